@@ -1,7 +1,6 @@
 // fmm.cu -- one FMM evaluation (the Poisson-solver call of Algorithm 3, Zhu 2017):
 // upward pass (P2M, M2M), dual tree walk (Algorithm 4) emitting blocks of unordered cell pairs,
-// mutual M2L and P2P (Sec. 2.1: F_AB = -F_BA), downward pass (L2L, L2P) and the
-// float64 direct summation (tg_direct_forces) that the force errors are measured against.
+// mutual M2L and P2P (Sec. 2.1: F_AB = -F_BA), downward pass (L2L, L2P).
 //
 // Expansions are Cartesian Taylor series truncated at total degree p, stored normalised by the
 // cell side s:
@@ -885,78 +884,6 @@ __global__ void zero_acc3(double *acc4, int64_t stride4, const int *dn)
     }
 }
 
-
-// ------------------------------------------------------------------ direct summation (float64)
-__global__ void direct_sum(int64_t n, const double *pos, const double *mass, const uint8_t *fast, int64_t n_sink,
-                           const int64_t *sink_idx, int kernel, double eps, double *acc, double *pot)
-{
-    __shared__ double sx[256], sy[256], sz[256], sm[256];
-    __shared__ uint8_t sf[256];
-    const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    const bool active = t < n_sink;
-    const int64_t i = active ? (sink_idx ? sink_idx[t] : t) : 0;
-    const double xi = active ? pos[i] : 0.0, yi = active ? pos[n + i] : 0.0, zi = active ? pos[2 * n + i] : 0.0;
-    const bool fi = active && fast && fast[i];
-    double ax = 0, ay = 0, az = 0, ph = 0;
-    const double eps2 = eps * eps;
-    for (int64_t j0 = 0; j0 < n; j0 += 256) {
-        const int64_t j = j0 + threadIdx.x;
-        if (j < n) {
-            sx[threadIdx.x] = pos[j];
-            sy[threadIdx.x] = pos[n + j];
-            sz[threadIdx.x] = pos[2 * n + j];
-            sm[threadIdx.x] = mass[j];
-            sf[threadIdx.x] = fast ? fast[j] : 0;
-        }
-        __syncthreads();
-        const int cnt = (int)((n - j0) < 256 ? (n - j0) : 256);
-        if (active) {
-            for (int q = 0; q < cnt; ++q) {
-                if (j0 + q == i) continue;
-                if (fi && sf[q]) continue;
-                const double dx = sx[q] - xi, dy = sy[q] - yi, dz = sz[q] - zi;
-                const double r2 = dx * dx + dy * dy + dz * dz;
-                double g, phi;
-                if (kernel == TG_KERNEL_PLUMMER) {
-                    const double s2 = r2 + eps2, inv = 1.0 / sqrt(s2);
-                    phi = -inv;
-                    g = inv * inv * inv;
-                } else if (r2 < eps2) {
-                    const double u = sqrt(r2) / eps, u2 = u * u, u3 = u2 * u, u4 = u2 * u2, u5 = u4 * u;
-                    phi = (3.0 * u4 * u3 - 15.0 * u3 * u3 + 28.0 * u5 - 21.0 * u4 + 7.0 * u2 - 3.0) / eps;
-                    g = (21.0 * u5 - 90.0 * u4 + 140.0 * u3 - 84.0 * u2 + 14.0) / (eps * eps2);
-                } else {
-                    const double inv = 1.0 / sqrt(r2);
-                    phi = -inv;
-                    g = inv * inv * inv;
-                }
-                ax += sm[q] * g * dx;
-                ay += sm[q] * g * dy;
-                az += sm[q] * g * dz;
-                ph += sm[q] * phi;
-            }
-        }
-        __syncthreads();
-    }
-    if (active) {
-        acc[t] = ax;
-        acc[n_sink + t] = ay;
-        acc[2 * n_sink + t] = az;
-        if (pot) pot[t] = ph;
-    }
-}
-
-tg_status direct_eval(tg_ctx *c, int64_t n, const double *pos, const double *mass, const uint8_t *fast,
-                      int64_t n_sink, const int64_t *sink_idx, double *acc, double *pot)
-{
-    if (n_sink <= 0) return TG_OK;
-    {
-        ProfScope ps_(c, TG_K_OTHER);
-        direct_sum<<<(int)((n_sink + 255) / 256), 256, 0, c->stream>>>(n, pos, mass, fast, n_sink, sink_idx,
-                                                                      c->prm.kernel, c->prm.eps, acc, pot);
-    }
-    return cuda_check(c, cudaGetLastError(), "direct summation");
-}
 
 // ------------------------------------------------------------------ orchestration
 __global__ void walk_init(uint2 *front, unsigned long long *front_ctr)

@@ -283,6 +283,7 @@ __global__ void radix_scatter(const uint64_t *keys_in, const uint32_t *vals_in, 
 tg_status fmm_eval(tg_ctx *c, int n, const double *pos, int64_t stride, const int64_t *sub,
                    const double *mass, const uint8_t *fast, double *acc, int64_t out_stride, double *pot,
                    bool keep_tree);
+// ---- direct.cu
 tg_status direct_eval(tg_ctx *c, int64_t n, const double *pos, const double *mass, const uint8_t *fast,
                       int64_t n_sink, const int64_t *sink_idx, double *acc, double *pot);
 
