@@ -1,14 +1,13 @@
 // direct.cu -- float64 direct summation for a sample of sinks (tg_direct_forces): the sum that force errors
 // are measured against.
 //
-// Bound by the float64 pipe: 16 operations per pair (18 with the potential).  The sinks are few (thousands)
+// Bound by the float64 pipe: 14 operations per pair (16 with the potential).  The sinks are few (thousands)
 // and the sources many, so the sources are split: a cluster of eight blocks takes a tile of up to 32
 // sinks, each block an eighth of the sources, and inside a block 256 / tile groups of threads take every
 // (256 / tile)-th source.  The partial sums are added in a fixed order, first in the block and then over the
 // cluster's shared memory, so no scratch memory is needed and two runs agree bit for bit.
 // 4096 sinks, 100,003 sources, with the potential: 193.3 ms with one thread per sink walking all sources (16 of
-// 152 SMs busy, 1/sqrt by the library), 15.5 ms in this form; 7.4e9 float64 operations at 2 per clock and SM
-// take 11.7 ms.
+// 152 SMs busy, 1/sqrt by the library), 13.7 ms in this form: 4.8e11 float64 operations per second.
 #include <cooperative_groups.h>
 
 #include "pair_f64.cuh"

@@ -995,22 +995,19 @@ static tg_status launch_m2l_t(tg_ctx *c, const TreeView &t, const M2LBlock *bloc
     (void)pot;   // the float64 contraction always includes the potential term
     return launch_m2l_f64(c, t, blocks, nblocks, Ms, L, p, nc, ncp, masked);
 }
-static tg_status launch_p2p_t(tg_ctx *c, const TreeView &t, const Geom *d_geom, const uint2 *pairs, int64_t npairs,
-                              const uint2 *self_pairs, int64_t nself, const float4 *pf, const uint8_t *fs,
-                              const int32_t *nslow, bool masked, bool pot, double *acc4)
+static tg_status launch_p2p_t(tg_ctx *c, const TreeView &t, const uint2 *pairs, int64_t npairs, const uint2 *self_pairs,
+                              int64_t nself, const float4 *pf, const double *const xyzm[4], const int32_t *nslow,
+                              bool pot, double *acc4)
 {
-    (void)d_geom;
-    (void)fs;
-    (void)masked;   // classes arrive as slow-first leaves (nslow)
+    (void)xyzm;
     return launch_p2p_f32(c, t, pairs, npairs, self_pairs, nself, pf, nslow, pot, acc4);
 }
-static tg_status launch_p2p_t(tg_ctx *c, const TreeView &t, const Geom *d_geom, const uint2 *pairs, int64_t npairs,
-                              const uint2 *self_pairs, int64_t nself, const dbl4 *pf, const uint8_t *fs,
-                              const int32_t *nslow, bool masked, bool pot, double *acc4)
+static tg_status launch_p2p_t(tg_ctx *c, const TreeView &t, const uint2 *pairs, int64_t npairs, const uint2 *self_pairs,
+                              int64_t nself, const dbl4 *pf, const double *const xyzm[4], const int32_t *nslow, bool pot,
+                              double *acc4)
 {
-    (void)nslow;   // the float64 tiles mask fast-fast pairs one by one
-    (void)pot;     // and always include the potential
-    return launch_p2p_f64(c, t, d_geom, pairs, npairs, self_pairs, nself, pf, fs, masked, acc4);
+    (void)pf;
+    return launch_p2p_f64(c, t, pairs, npairs, self_pairs, nself, xyzm, nslow, pot, acc4);
 }
 
 template <class T, class T4>
@@ -1122,8 +1119,8 @@ static tg_status eval_typed(tg_ctx *c, int n, int ncell, const TreeView &t, cons
         }
 #undef TG_L2P
     }
-    if ((st = launch_p2p_t(c, t, d_geom, p2p, n_p2p, p2p + (c->p2p_cap - n_self), n_self, pf, fs, nslow, masked,
-                            want_pot, acc4)))
+    const double *const xyzm[4] = {xs, ys, zs, ms};
+    if ((st = launch_p2p_t(c, t, p2p, n_p2p, p2p + (c->p2p_cap - n_self), n_self, pf, xyzm, nslow, want_pot, acc4)))
         return st;
     return cuda_check(c, cudaGetLastError(), "fmm evaluation");
 }
@@ -1261,6 +1258,24 @@ tg_status mac_params_upload(tg_ctx *c)
     return cuda_check(c, cudaMemcpy(mpd, &mp, sizeof(mp), cudaMemcpyHostToDevice), "criterion upload");
 }
 
+static tg_status launch_p2p_dev_t(tg_ctx *c, const TreeView &t, const DevEval *de, const Geom *gp,
+                                  const unsigned long long *wctr, const uint2 *p2p, size_t cap_p2p, int cap_cells,
+                                  const float4 *pf, const double *const xyzm[4], const int32_t *nslow, double *acc4,
+                                  int stride)
+{
+    (void)xyzm;
+    return launch_p2p_f32_dev(c, t, de, gp, wctr, p2p, cap_p2p, cap_cells, pf, nslow, acc4, stride, B_SCAN_TMP2);
+}
+static tg_status launch_p2p_dev_t(tg_ctx *c, const TreeView &t, const DevEval *de, const Geom *gp,
+                                  const unsigned long long *wctr, const uint2 *p2p, size_t cap_p2p, int cap_cells,
+                                  const dbl4 *pf, const double *const xyzm[4], const int32_t *nslow, double *acc4,
+                                  int stride)
+{
+    (void)gp;
+    (void)pf;
+    return launch_p2p_f64_dev(c, t, de, wctr, p2p, cap_p2p, cap_cells, xyzm, nslow, acc4, stride, B_SCAN_TMP2);
+}
+
 template <class T, class T4>
 static tg_status fmm_eval_dev_t(tg_ctx *c, DevEval *de, const BatchCaps &cap, const double *xin, const double *min,
                                 const uint8_t *fin, double *acc, unsigned long long *stats)
@@ -1346,35 +1361,31 @@ static tg_status fmm_eval_dev_t(tg_ctx *c, DevEval *de, const BatchCaps &cap, co
         ProfScope ps_(c, TG_K_UP);
         leaf_particles<T4><<<gcell, 256, 0, c->stream>>>(t, d_geom, xs2, ys2, zs2, ms2, pf, leaf_of);
     }
-    // float32: P2P needs only the walk's lists and the leaf offsets, so it runs on the side stream (after
-    // the walk) beside the moments, M2L and the downward pass, into its own sums (acc4p, added by
-    // scatter_out); its scan takes its own scratch slot.  The forks and joins are events, which a stream
-    // capture turns into graph edges.
+    // P2P needs only the walk's lists and the leaf offsets, so it runs on the side stream (after the walk) beside
+    // the moments, M2L and the downward pass, into its own sums (acc4p, added by scatter_out); its scan takes
+    // its own scratch slot.  The forks and joins are events, which a stream capture turns into graph edges.
     double *acc4p = nullptr;
-    const bool fork = sizeof(T) == 4;
-    if (fork) {
-        if ((st = ensure_t(c, B_ACC_P2P, (size_t)4 * cap.n, &acc4p))) {
-            cudaStreamWaitEvent(c->stream, c->ev_walk, 0);
-            return st;
-        }
-        cudaEventRecord(c->ev_fork, c->stream);   // the leaf offsets; the side stream is past the walk
-        cudaStreamWaitEvent(c->side, c->ev_fork, 0);
+    if ((st = ensure_t(c, B_ACC_P2P, (size_t)4 * cap.n, &acc4p))) {
+        cudaStreamWaitEvent(c->stream, c->ev_walk, 0);
+        return st;
+    }
+    cudaEventRecord(c->ev_fork, c->stream);   // the leaf offsets; the side stream is past the walk
+    cudaStreamWaitEvent(c->side, c->ev_fork, 0);
+    {
         cudaStream_t main_stream = c->stream;
         c->stream = c->side;
         {
             ProfScope ps_(c, TG_K_OTHER);
             zero_acc3<<<c->num_sms * 4, 256, 0, c->stream>>>(acc4p, cap.n, &de->n);
         }
-        st = launch_p2p_f32_dev(c, t, de, d_geom, wctr, p2p, cap.p2p, cap.cells, reinterpret_cast<const float4 *>(pf),
-                                nslow, acc4p, cap.n, B_SCAN_TMP2);
+        const double *const xyzm[4] = {xs2, ys2, zs2, ms2};
+        st = launch_p2p_dev_t(c, t, de, d_geom, wctr, p2p, cap.p2p, cap.cells, pf, xyzm, nslow, acc4p, cap.n);
         c->stream = main_stream;
-        cudaEventRecord(c->ev_join, c->side);
-        if (st) {
-            cudaStreamWaitEvent(c->stream, c->ev_join, 0);
-            return st;
-        }
-    } else {
-        cudaEventRecord(c->ev_join, c->side);   // float64: P2P follows on the main stream
+    }
+    cudaEventRecord(c->ev_join, c->side);
+    if (st) {
+        cudaStreamWaitEvent(c->stream, c->ev_join, 0);
+        return st;
     }
     {
         ProfScope ps_(c, TG_K_UP);
@@ -1428,9 +1439,6 @@ static tg_status fmm_eval_dev_t(tg_ctx *c, DevEval *de, const BatchCaps &cap, co
         }
     }
     cudaStreamWaitEvent(c->stream, c->ev_join, 0);
-    if (!fork && (st = launch_p2p_f64_dev(c, t, d_geom, wctr, p2p, cap.p2p, reinterpret_cast<const dbl4 *>(pf), fs2, acc4,
-                                         cap.n)))
-        return st;
     {
         ProfScope ps_(c, TG_K_DOWN);
         scatter_out<<<grid_for(cap.n, 256), 256, 0, c->stream>>>(cap.n, perm2, acc4, acc, cap.n, nullptr, &de->n, cap.n,

@@ -690,7 +690,7 @@ static tg_status hold_presize(tg_ctx *c, const Sched &s, const BatchCaps &cap, c
     const size_t rows = (size_t)C * 2;
     const int nblocks = (n + kSortTileItems - 1) / kSortTileItems;
     const int nh = (p_ + 1) * (p_ + 1), ncpr = (nh + 3) & ~3;
-    const int64_t max_units = (int64_t)cap.p2p / 16 + C + 1;
+    const int64_t max_units = (int64_t)cap.p2p / 8 + std::min<int64_t>((int64_t)cap.p2p, 32768) + C + 1;   // own_max_units
     const size_t tsz = c->prm.precision == TG_PREC_FP32 ? 4 : 8;   // compute precision
     struct Need { int slot; size_t bytes; };
     const Need needs[] = {

@@ -8,7 +8,7 @@
 // row/column pair the kernel value is computed once and applied to both particles, with opposite
 // signs (Sec. 2.1, Eq. 2).  Rows keep their sums in registers and flush them once per chunk.
 // Columns combine their partials with a warp reduce-scatter into shared memory, and flush them
-// once per work unit (kOwnUnit partners of the owner; the units of all owners are handed out
+// once per work unit (own_unit partners of the owner; the units of all owners are handed out
 // dynamically to the warps).
 //
 // With slow/fast classes the leaves hold their slow particles first.  Slow rows meet every
@@ -19,11 +19,26 @@
 // than eps to the owner's come first; chunks made only of the other partners' rows need no softening
 // test, the others take the pair value at max(r, eps) and correct the rare pairs with r < eps.
 #pragma once
+#include <algorithm>
+
 #include "p2p_tile.cuh"
 
 namespace tg {
 
-constexpr int kOwnUnit = 32;   // partners per work unit of the owner kernel (one per lane)
+// Partners per work unit of the owner kernels (a power of two, at most one per lane).  Large units pack more rows
+// densely.  Float64 pairs take 64 times as long on the same warps, so there the units are cut until there are at
+// least 8192 of them, about four per warp.  Measured with at least 1024 / 2048 / 4096 / 8192 units: 1.13 / 0.81 /
+// 0.60 / 0.58 ms for a 4096-particle Plummer sphere (21,772 leaf pairs), 17.5 / 17.6 / 17.5 / 17.2 ms for a
+// 100,003-particle sphere (255,859).
+__host__ __device__ __forceinline__ int own_unit(int64_t npairs, bool f64)
+{
+    if (!f64) return 32;
+    int u = 1;
+    while (u < 32 && ((int64_t)u << 14) < npairs) u <<= 1;
+    return u;
+}
+// capacity of the unit list: every owner opens one unit more than its full ones
+inline int64_t own_max_units(int64_t npairs, int64_t ncell) { return npairs / 8 + std::min<int64_t>(npairs, 32768) + ncell + 1; }
 
 // Owner and partner of each distinct leaf pair, and per-owner partner counts (own_cnt starts at zero).
 // The walk writes the pairs of one row cell side by side, so lanes of a warp often share an owner:
@@ -48,15 +63,16 @@ __global__ void p2p_owner_count(const uint2 *__restrict__ pairs, int64_t npairs,
     }
 }
 
-// Partners grouped by owner: partners[own_off[B] .. own_off[B] + own_cnt[B]).  Every kOwnUnit-th
+// Partners grouped by owner: partners[own_off[B] .. own_off[B] + own_cnt[B]).  Every own_unit-th
 // partner of an owner also opens a work unit (owner, position); ctr[0] counts the units.
 // own_fill and ctr start at zero.  Lanes with equal owners take consecutive slots with one atomic, and
 // the units a warp opens are reserved with one atomic on ctr[0] (whole warps iterate together).
 __global__ void p2p_owner_fill(const uint2 *__restrict__ tagged, int64_t npairs, const uint32_t *__restrict__ own_off,
                                uint32_t *own_fill, int32_t *partners, uint2 *units, uint32_t *ctr,
-                               const unsigned long long *dnp)
+                               const unsigned long long *dnp, bool f64)
 {
     if (dnp) npairs = (int64_t)*dnp;
+    const uint32_t unit = (uint32_t)own_unit(npairs, f64);
     const int lane = threadIdx.x & 31;
     const unsigned lt = (1u << lane) - 1u;
     const int64_t stride = (int64_t)gridDim.x * blockDim.x;
@@ -72,7 +88,7 @@ __global__ void p2p_owner_fill(const uint2 *__restrict__ tagged, int64_t npairs,
         base = __shfl_sync(0xffffffffu, base, leader);
         const uint32_t f = base + (uint32_t)__popc(peers & lt);
         if (valid) partners[own_off[op.x] + f] = (int32_t)op.y;
-        const bool opens = valid && f % kOwnUnit == 0;
+        const bool opens = valid && (f & (unit - 1u)) == 0;
         const unsigned ob = __ballot_sync(0xffffffffu, opens);
         uint32_t ubase = 0u;
         if (lane == 0 && ob) ubase = atomicAdd(&ctr[0], (uint32_t)__popc(ob));
@@ -301,7 +317,7 @@ __device__ __forceinline__ int warp_incl_scan(int v, int lane)
     return v;
 }
 
-// One warp per work unit (kOwnUnit partners of one owner), units taken from a shared counter
+// One warp per work unit (own_unit partners of one owner), units taken from a shared counter
 // (ctr[1], starts at zero) so that the load stays balanced whatever the spread of leaf work.  After
 // the units, the same counter hands out the self pairs (A, A): slow rows of A against every particle
 // of A with a larger index, i.e. each slow-slow and slow-fast pair once (p2p_pair_f32, SELF).
@@ -311,7 +327,7 @@ template <int KERNEL, int ROWS, bool POT>
 __global__ void __launch_bounds__(256, 2) p2p_owner_f32(TreeView t, int log2L, const uint2 *__restrict__ units,
                                                         uint32_t *ctr, const uint32_t *__restrict__ own_off,
                                                         const uint32_t *__restrict__ own_cnt,
-                                                        const int32_t *__restrict__ partners,
+                                                        const int32_t *__restrict__ partners, int64_t npairs,
                                                         const uint2 *__restrict__ self_pairs, uint32_t nself,
                                                         const float4 *__restrict__ pf, const int32_t *__restrict__ nslow,
                                                         float eps, double *acc4, int n, unsigned long long *pair_counter,
@@ -320,10 +336,11 @@ __global__ void __launch_bounds__(256, 2) p2p_owner_f32(TreeView t, int log2L, c
 {
     if (walk_ctr) {
         log2L = gp->log2L;
+        npairs = (int64_t)walk_ctr[2];
         nself = (uint32_t)walk_ctr[4];
         self_pairs = p2p_base + (cap_p2p - nself);
     }
-    static_assert(kOwnUnit <= 32, "one partner per lane");
+    const int unit = own_unit(npairs, false);
     __shared__ OwnerShared sh;
     const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
     const unsigned lt = (1u << lane) - 1u;
@@ -354,7 +371,7 @@ __global__ void __launch_bounds__(256, 2) p2p_owner_f32(TreeView t, int log2L, c
         const int cnt = (int)own_cnt[B], base = (int)own_off[B];
         const int fb = t.first[B], nb = t.count[B], sB = nslow ? nslow[B] : nb, lB = t.level[B];
         {
-            const int np = min(kOwnUnit, cnt - pb);
+            const int np = min(unit, cnt - pb);
             int fa = 0, na = 0, sa = 0;
             float4 off = make_float4(0.f, 0.f, 0.f, 0.f);
             bool near = false;
@@ -479,38 +496,85 @@ __global__ void zero_u32_dev(uint32_t *p, const int *n32, int extra)
     for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) p[i] = 0u;
 }
 
+// The distinct leaf pairs grouped by owner (both precisions).
+struct OwnerLists {
+    uint2 *units = nullptr;
+    uint32_t *ctr = nullptr, *off = nullptr, *cnt = nullptr;   // ctr: [0] work units, [1] next unit to take
+    int32_t *partners = nullptr;
+};
+
+static tg_status owner_lists(tg_ctx *c, const TreeView &t, const uint2 *pairs, int64_t npairs, bool f64, OwnerLists *o)
+{
+    tg_status st;
+    const int ncell = t.ncell;
+    uint32_t *own_fill;
+    uint2 *tagged;
+    const int64_t max_units = own_max_units(npairs, ncell);
+    if ((st = ensure_t(c, B_OWN_CNT, (size_t)ncell + 2, &o->cnt)) || (st = ensure_t(c, B_OWN_FILL, ncell, &own_fill)) ||
+        (st = ensure_t(c, B_OWN_OFF, ncell, &o->off)) || (st = ensure_t(c, B_OWN_LIST, max_units, &o->units)) ||
+        (st = ensure_t(c, B_OWN_TAG, npairs, &tagged)) || (st = ensure_t(c, B_OWN_PART, npairs, &o->partners)))
+        return st;
+    o->ctr = o->cnt + ncell;
+    cudaMemsetAsync(o->cnt, 0, sizeof(uint32_t) * ((size_t)ncell + 2), c->stream);
+    cudaMemsetAsync(own_fill, 0, sizeof(uint32_t) * (size_t)ncell, c->stream);
+    if (npairs > 0) {
+        {
+            ProfScope ps_(c, TG_K_OTHER);
+            p2p_owner_count<<<grid_for(npairs, 256), 256, 0, c->stream>>>(pairs, npairs, t.count, o->cnt, tagged, nullptr);
+        }
+        if ((st = exclusive_scan_u32(c, o->cnt, o->off, ncell, nullptr))) return st;
+        {
+            ProfScope ps_(c, TG_K_OTHER);
+            p2p_owner_fill<<<grid_for(npairs, 256), 256, 0, c->stream>>>(tagged, npairs, o->off, own_fill, o->partners,
+                                                                         o->units, o->ctr, nullptr, f64);
+        }
+    }
+    return cuda_check(c, cudaGetLastError(), "p2p owner lists");
+}
+
+// The same with every size on the device (batched HOLD step): the pair count comes from the walk's counters, the
+// cell count from de; buffers are sized for the capacities.
+static tg_status owner_lists_dev(tg_ctx *c, const TreeView &t, const DevEval *de, const unsigned long long *walk_ctr,
+                                 const uint2 *p2p, size_t cap_p2p, int cap_cells, int scan_scratch, bool f64,
+                                 OwnerLists *o)
+{
+    tg_status st;
+    uint32_t *own_fill;
+    uint2 *tagged;
+    const int64_t max_units = own_max_units((int64_t)cap_p2p, cap_cells);
+    if ((st = ensure_t(c, B_OWN_CNT, (size_t)cap_cells + 2, &o->cnt)) ||
+        (st = ensure_t(c, B_OWN_FILL, (size_t)cap_cells + 2, &own_fill)) ||
+        (st = ensure_t(c, B_OWN_OFF, (size_t)cap_cells, &o->off)) || (st = ensure_t(c, B_OWN_LIST, max_units, &o->units)) ||
+        (st = ensure_t(c, B_OWN_TAG, cap_p2p, &tagged)) || (st = ensure_t(c, B_OWN_PART, cap_p2p, &o->partners)))
+        return st;
+    o->ctr = own_fill + cap_cells;
+    const int g = c->num_sms * 4;
+    {
+        ProfScope ps_(c, TG_K_OTHER);
+        zero_u32_dev<<<g, 256, 0, c->stream>>>(o->cnt, &de->ncell, 0);
+        zero_u32_dev<<<g, 256, 0, c->stream>>>(own_fill, &de->ncell, 0);
+        zero_u32_dev<<<1, 32, 0, c->stream>>>(o->ctr, nullptr, 2);
+        p2p_owner_count<<<g, 256, 0, c->stream>>>(p2p, (int64_t)cap_p2p, t.count, o->cnt, tagged, walk_ctr + 2);
+    }
+    if ((st = exclusive_scan_u32(c, o->cnt, o->off, cap_cells, nullptr, &de->ncell, scan_scratch))) return st;
+    {
+        ProfScope ps_(c, TG_K_OTHER);
+        p2p_owner_fill<<<g, 256, 0, c->stream>>>(tagged, (int64_t)cap_p2p, o->off, own_fill, o->partners, o->units, o->ctr,
+                                                  walk_ctr + 2, f64);
+    }
+    return cuda_check(c, cudaGetLastError(), "p2p owner lists (device sizes)");
+}
+
 // Every P2P pair in float32, one launch: the distinct leaf pairs grouped by owner, then the self pairs.
 // pot = false: accelerations only (the potential slot of acc4 is left out).
 tg_status launch_p2p_f32(tg_ctx *c, const TreeView &t, const uint2 *pairs, int64_t npairs, const uint2 *self_pairs,
                          int64_t nself, const float4 *pf, const int32_t *nslow, bool pot, double *acc4)
 {
-    tg_status st;
-    const int ncell = t.ncell;
-    uint32_t *own_cnt, *own_fill, *own_off;
-    uint2 *tagged, *units;
-    int32_t *partners;
     if (npairs + nself == 0) return TG_OK;
     if (nself > 0xffffffffll) return set_err(c, TG_ERR_CAPACITY, "too many self pairs for one P2P launch");
-    const int64_t max_units = npairs / kOwnUnit + ncell + 1;
-    if ((st = ensure_t(c, B_OWN_CNT, (size_t)ncell + 2, &own_cnt)) || (st = ensure_t(c, B_OWN_FILL, ncell, &own_fill)) ||
-        (st = ensure_t(c, B_OWN_OFF, ncell, &own_off)) || (st = ensure_t(c, B_OWN_LIST, max_units, &units)) ||
-        (st = ensure_t(c, B_OWN_TAG, npairs, &tagged)) || (st = ensure_t(c, B_OWN_PART, npairs, &partners)))
-        return st;
-    uint32_t *ctr = own_cnt + ncell;   // [0] work units, [1] next unit to take
-    cudaMemsetAsync(own_cnt, 0, sizeof(uint32_t) * ((size_t)ncell + 2), c->stream);
-    cudaMemsetAsync(own_fill, 0, sizeof(uint32_t) * (size_t)ncell, c->stream);
-    if (npairs > 0) {
-        {
-            ProfScope ps_(c, TG_K_OTHER);
-            p2p_owner_count<<<grid_for(npairs, 256), 256, 0, c->stream>>>(pairs, npairs, t.count, own_cnt, tagged, nullptr);
-        }
-        if ((st = exclusive_scan_u32(c, own_cnt, own_off, ncell, nullptr))) return st;
-        {
-            ProfScope ps_(c, TG_K_OTHER);
-            p2p_owner_fill<<<grid_for(npairs, 256), 256, 0, c->stream>>>(tagged, npairs, own_off, own_fill, partners,
-                                                                         units, ctr, nullptr);
-        }
-    }
+    OwnerLists o;
+    tg_status st = owner_lists(c, t, pairs, npairs, false, &o);
+    if (st) return st;
     const float eps = (float)c->prm.eps;
     unsigned long long *pc = c->d_counters;
     const bool plummer = c->prm.kernel == TG_KERNEL_PLUMMER;
@@ -518,8 +582,8 @@ tg_status launch_p2p_f32(tg_ctx *c, const TreeView &t, const uint2 *pairs, int64
     const int rows = c->tune.p2p_rows;
     const int grid = c->num_sms * owner_occupancy(rows);
 #define TG_OWNER(K, R, PT)                                                                                        \
-    p2p_owner_f32<K, R, PT><<<grid, 256, 0, c->stream>>>(t, c->walk_log2L, units, ctr, own_off, own_cnt, partners,  \
-                                                         self_pairs, (uint32_t)nself, pf, nslow, eps, acc4, t.n, pc,    \
+    p2p_owner_f32<K, R, PT><<<grid, 256, 0, c->stream>>>(t, c->walk_log2L, o.units, o.ctr, o.off, o.cnt, o.partners, \
+                                                         npairs, self_pairs, (uint32_t)nself, pf, nslow, eps, acc4, t.n, pc,    \
                                                          nullptr, nullptr, nullptr, 0ull)
 #define TG_OWNER_ROWS(K, PT)                                                                                      \
     switch (rows) {                                                                                               \
@@ -545,31 +609,9 @@ tg_status launch_p2p_f32_dev(tg_ctx *c, const TreeView &t, const DevEval *de, co
                              const unsigned long long *walk_ctr, const uint2 *p2p, size_t cap_p2p, int cap_cells,
                              const float4 *pf, const int32_t *nslow, double *acc4, int stride, int scan_scratch)
 {
-    tg_status st;
-    uint32_t *own_cnt, *own_fill, *own_off, *ctr;
-    uint2 *tagged, *units;
-    int32_t *partners;
-    const int64_t max_units = (int64_t)cap_p2p / kOwnUnit + cap_cells + 1;
-    if ((st = ensure_t(c, B_OWN_CNT, (size_t)cap_cells + 2, &own_cnt)) ||
-        (st = ensure_t(c, B_OWN_FILL, (size_t)cap_cells + 2, &own_fill)) ||
-        (st = ensure_t(c, B_OWN_OFF, (size_t)cap_cells, &own_off)) || (st = ensure_t(c, B_OWN_LIST, max_units, &units)) ||
-        (st = ensure_t(c, B_OWN_TAG, cap_p2p, &tagged)) || (st = ensure_t(c, B_OWN_PART, cap_p2p, &partners)))
-        return st;
-    ctr = own_fill + cap_cells;   // [0] work units, [1] next unit to take
-    const int g = c->num_sms * 4;
-    {
-        ProfScope ps_(c, TG_K_OTHER);
-        zero_u32_dev<<<g, 256, 0, c->stream>>>(own_cnt, &de->ncell, 0);
-        zero_u32_dev<<<g, 256, 0, c->stream>>>(own_fill, &de->ncell, 0);
-        zero_u32_dev<<<1, 32, 0, c->stream>>>(ctr, nullptr, 2);
-        p2p_owner_count<<<g, 256, 0, c->stream>>>(p2p, (int64_t)cap_p2p, t.count, own_cnt, tagged, walk_ctr + 2);
-    }
-    if ((st = exclusive_scan_u32(c, own_cnt, own_off, cap_cells, nullptr, &de->ncell, scan_scratch))) return st;
-    {
-        ProfScope ps_(c, TG_K_OTHER);
-        p2p_owner_fill<<<g, 256, 0, c->stream>>>(tagged, (int64_t)cap_p2p, own_off, own_fill, partners, units, ctr,
-                                                  walk_ctr + 2);
-    }
+    OwnerLists o;
+    tg_status st = owner_lists_dev(c, t, de, walk_ctr, p2p, cap_p2p, cap_cells, scan_scratch, false, &o);
+    if (st) return st;
     const float eps = (float)c->prm.eps;
     unsigned long long *pc = c->d_counters;
     const bool plummer = c->prm.kernel == TG_KERNEL_PLUMMER;
@@ -577,7 +619,7 @@ tg_status launch_p2p_f32_dev(tg_ctx *c, const TreeView &t, const DevEval *de, co
     const int rows = c->tune.p2p_rows;
     const int grid = c->num_sms * owner_occupancy(rows);
 #define TG_OWNER_DEV(K, R)                                                                                        \
-    p2p_owner_f32<K, R, false><<<grid, 256, 0, c->stream>>>(t, 0, units, ctr, own_off, own_cnt, partners, nullptr, 0u, \
+    p2p_owner_f32<K, R, false><<<grid, 256, 0, c->stream>>>(t, 0, o.units, o.ctr, o.off, o.cnt, o.partners, 0, nullptr, 0u, \
                                                             pf, nslow, eps, acc4, stride, pc, gp, walk_ctr, p2p,    \
                                                             (unsigned long long)cap_p2p)
 #define TG_OWNER_DEV_ROWS(K)                                                                                      \

@@ -9,109 +9,6 @@
 
 namespace tg {
 
-constexpr int kP2PThreads = 64;
-
-// Batched path (walk_ctr non-null): the distinct leaf pairs [0, walk_ctr[2]) and the walk_ctr[4] self
-// pairs at the end of the buffer (capacity cap_p2p) in one launch.
-template <class T, class T4, bool MASKED, int KERNEL>
-__global__ void __launch_bounds__(kP2PThreads) p2p_mutual(TreeView t, const Geom *gp, const uint2 *pairs,
-                                                          int64_t npairs, const T4 *pf, const uint8_t *fs, T eps,
-                                                          double *acc4, int n, unsigned long long *pair_counter,
-                                                          const unsigned long long *walk_ctr = nullptr,
-                                                          unsigned long long cap_p2p = 0)
-{
-    int64_t ndist = npairs, self0 = 0;
-    if (walk_ctr) {
-        ndist = (int64_t)walk_ctr[2];
-        self0 = (int64_t)(cap_p2p - walk_ctr[4]);
-        npairs = ndist + (int64_t)walk_ctr[4];
-    }
-    __shared__ T4 sb[kMaxNcrit];
-    __shared__ uint8_t sfb[kMaxNcrit];
-    __shared__ T colacc[kMaxNcrit][4];
-    const Geom g = *gp;
-    const int lane = threadIdx.x & 31;
-    const T eps2 = eps * eps, inv_eps = T(1) / eps, inv_eps3 = inv_eps * inv_eps * inv_eps;
-    unsigned long long my_pairs = 0;
-    for (int64_t w = blockIdx.x; w < npairs; w += gridDim.x) {
-        const uint2 pr = pairs[w < ndist ? w : self0 + (w - ndist)];
-        const int a = (int)pr.x, b = (int)pr.y;
-        const int fa = t.first[a], na = t.count[a], fb = t.first[b], nb = t.count[b];
-        const double sb_side = ldexp(g.L, -(int)t.level[b]), sa_side = ldexp(g.L, -(int)t.level[a]);
-        const T ox = (T)(((double)t.cx[b] + 0.5) * sb_side - ((double)t.cx[a] + 0.5) * sa_side);
-        const T oy = (T)(((double)t.cy[b] + 0.5) * sb_side - ((double)t.cy[a] + 0.5) * sa_side);
-        const T oz = (T)(((double)t.cz[b] + 0.5) * sb_side - ((double)t.cz[a] + 0.5) * sa_side);
-        const bool self = a == b;
-        // B is staged in chunks of kMaxNcrit (leaves at the deepest level may exceed n_crit)
-        for (int j0 = 0; j0 < nb; j0 += kMaxNcrit) {
-            const int nbc = min(kMaxNcrit, nb - j0);
-            __syncthreads();
-            for (int j = threadIdx.x; j < nbc; j += blockDim.x) {
-                T4 v = pf[fb + j0 + j];
-                v.x += ox;
-                v.y += oy;
-                v.z += oz;
-                sb[j] = v;
-                sfb[j] = MASKED ? fs[fb + j0 + j] : 0;
-                colacc[j][0] = colacc[j][1] = colacc[j][2] = colacc[j][3] = T(0);
-            }
-            __syncthreads();
-            for (int i0 = 0; i0 < na; i0 += blockDim.x) {
-                const int i = i0 + threadIdx.x;
-                const bool row = i < na;
-                T4 pi;
-                if (row) pi = pf[fa + i];
-                else pi.x = pi.y = pi.z = pi.w = T(0);
-                const uint8_t fi = (MASKED && row) ? fs[fa + i] : 0;
-                T rax = 0, ray = 0, raz = 0, rph = 0;
-                for (int j = 0; j < nbc; ++j) {
-                    const T4 pj = sb[j];
-                    const bool use = row && (!self || j0 + j > i) && !(MASKED && fi && sfb[j]);
-                    const T dx = pj.x - pi.x, dy = pj.y - pi.y, dz = pj.z - pi.z;
-                    const T r2 = dx * dx + dy * dy + dz * dz;
-                    T gk, ph;
-                    pair_kernel<T, KERNEL>(use ? r2 : T(1), eps, eps2, inv_eps, inv_eps3, gk, ph);
-                    if (!use) {
-                        gk = T(0);
-                        ph = T(0);
-                    }
-                    my_pairs += use ? 1 : 0;
-                    rax += pj.w * gk * dx;
-                    ray += pj.w * gk * dy;
-                    raz += pj.w * gk * dz;
-                    rph += pj.w * ph;
-                    T cx = -pi.w * gk * dx, cy = -pi.w * gk * dy, cz = -pi.w * gk * dz, cp = pi.w * ph;
-                    cx = warp_sum(cx);
-                    cy = warp_sum(cy);
-                    cz = warp_sum(cz);
-                    cp = warp_sum(cp);
-                    if (lane == 0) {
-                        atomicAdd(&colacc[j][0], cx);
-                        atomicAdd(&colacc[j][1], cy);
-                        atomicAdd(&colacc[j][2], cz);
-                        atomicAdd(&colacc[j][3], cp);
-                    }
-                }
-                if (row) {
-                    atomicAdd(&acc4[fa + i], (double)rax);
-                    atomicAdd(&acc4[(size_t)n + fa + i], (double)ray);
-                    atomicAdd(&acc4[2 * (size_t)n + fa + i], (double)raz);
-                    atomicAdd(&acc4[3 * (size_t)n + fa + i], (double)rph);
-                }
-            }
-            __syncthreads();
-            for (int j = threadIdx.x; j < nbc; j += blockDim.x) {
-                atomicAdd(&acc4[fb + j0 + j], (double)colacc[j][0]);
-                atomicAdd(&acc4[(size_t)n + fb + j0 + j], (double)colacc[j][1]);
-                atomicAdd(&acc4[2 * (size_t)n + fb + j0 + j], (double)colacc[j][2]);
-                atomicAdd(&acc4[3 * (size_t)n + fb + j0 + j], (double)colacc[j][3]);
-            }
-        }
-    }
-    my_pairs = warp_sum(my_pairs);
-    if (lane == 0 && my_pairs) atomicAdd(pair_counter, my_pairs);
-}
-
 // ------------------------------------------------------------------ float32 warp tiles
 // Building blocks of the float32 P2P launch (p2p_owner.cuh): the pair value and the tile of one
 // leaf pair, used there for the self pairs (A, A).
@@ -234,58 +131,6 @@ __device__ __noinline__ void p2p_pair_f32(const float4 *__restrict__ pf, int fa,
                         atomicAdd(&acc4[(size_t)comp * n + fa + ir[r]], f2d_exact(ra[r][comp]));
         }
     }
-}
-
-template <class T, class T4>
-static tg_status launch_p2p_generic(tg_ctx *c, const TreeView &t, const Geom *d_geom, const uint2 *pairs, int64_t npairs,
-                            const T4 *pf, const uint8_t *fs, bool masked, double *acc4)
-{
-    const int grid = (int)std::min<int64_t>(npairs, (int64_t)c->num_sms * 16);
-    const T eps = (T)c->prm.eps;
-    unsigned long long *ctr = c->d_counters;
-    const int kern = c->prm.kernel;
-    ProfScope ps_(c, TG_K_P2P);
-#define TG_P2P_LAUNCH(M, K) \
-    p2p_mutual<T, T4, M, K><<<grid, kP2PThreads, 0, c->stream>>>(t, d_geom, pairs, npairs, pf, fs, eps, acc4, t.n, ctr)
-    if (masked) {
-        if (kern == TG_KERNEL_PLUMMER) TG_P2P_LAUNCH(true, TG_KERNEL_PLUMMER);
-        else TG_P2P_LAUNCH(true, TG_KERNEL_WENDLAND_C2);
-    } else {
-        if (kern == TG_KERNEL_PLUMMER) TG_P2P_LAUNCH(false, TG_KERNEL_PLUMMER);
-        else TG_P2P_LAUNCH(false, TG_KERNEL_WENDLAND_C2);
-    }
-#undef TG_P2P_LAUNCH
-    return cuda_check(c, cudaGetLastError(), "p2p launch");
-}
-
-// float64 P2P with every count on the device (batched path): one launch over the distinct and self pairs
-tg_status launch_p2p_f64_dev(tg_ctx *c, const TreeView &t, const Geom *d_geom, const unsigned long long *walk_ctr,
-                             const uint2 *p2p, size_t cap_p2p, const dbl4 *pf, const uint8_t *fs, double *acc4, int stride)
-{
-    const int grid = c->num_sms * 16;
-    const double eps = c->prm.eps;
-    ProfScope ps_(c, TG_K_P2P);
-    if (c->prm.kernel == TG_KERNEL_PLUMMER)
-        p2p_mutual<double, dbl4, true, TG_KERNEL_PLUMMER><<<grid, kP2PThreads, 0, c->stream>>>(
-            t, d_geom, p2p, 0, pf, fs, eps, acc4, stride, c->d_counters, walk_ctr, (unsigned long long)cap_p2p);
-    else
-        p2p_mutual<double, dbl4, true, TG_KERNEL_WENDLAND_C2><<<grid, kP2PThreads, 0, c->stream>>>(
-            t, d_geom, p2p, 0, pf, fs, eps, acc4, stride, c->d_counters, walk_ctr, (unsigned long long)cap_p2p);
-    return cuda_check(c, cudaGetLastError(), "p2p launch (device sizes, float64)");
-}
-
-// float64 P2P: one block per leaf pair, the distinct pairs then the self pairs (the tile tells them
-// apart at run time and masks fast-fast pairs one by one); float32 goes through p2p_owner.cuh.
-tg_status launch_p2p_f64(tg_ctx *c, const TreeView &t, const Geom *d_geom, const uint2 *pairs, int64_t npairs,
-                         const uint2 *self_pairs, int64_t nself, const dbl4 *pf, const uint8_t *fs, bool masked,
-                         double *acc4)
-{
-    tg_status st;
-    if (npairs > 0 && (st = launch_p2p_generic<double, dbl4>(c, t, d_geom, pairs, npairs, pf, fs, masked, acc4)))
-        return st;
-    if (nself > 0 && (st = launch_p2p_generic<double, dbl4>(c, t, d_geom, self_pairs, nself, pf, fs, masked, acc4)))
-        return st;
-    return TG_OK;
 }
 
 }  // namespace tg

@@ -243,8 +243,6 @@ tg_status launch_m2l_f32_dev(tg_ctx *c, const TreeView &t, const DevEval *de, co
 tg_status launch_m2l_f64_dev(tg_ctx *c, const TreeView &t, const DevEval *de, const Geom *gp, const M2LBlock *blocks,
                              const unsigned long long *dnb, int64_t cap_blocks, const double *Ms, double *L, int p,
                              int ncp);
-tg_status launch_p2p_f64_dev(tg_ctx *c, const TreeView &t, const Geom *d_geom, const unsigned long long *walk_ctr,
-                             const uint2 *p2p, size_t cap_p2p, const dbl4 *pf, const uint8_t *fs, double *acc4, int stride);
 tg_status launch_m2l_f64(tg_ctx *c, const TreeView &t, const M2LBlock *blocks, int64_t nblocks, const double *Ms,
                          double *L, int p, int nc, int ncp, bool masked);
 // ---- p2p.cu: mutual P2P of all leaf pairs (distinct pairs and self pairs) into acc4.
@@ -254,9 +252,12 @@ tg_status launch_p2p_f32_dev(tg_ctx *c, const TreeView &t, const DevEval *de, co
                              const unsigned long long *walk_ctr, const uint2 *p2p, size_t cap_p2p, int cap_cells,
                              const float4 *pf, const int32_t *nslow, double *acc4, int stride,
                              int scan_scratch = B_SCAN_TMP);
-tg_status launch_p2p_f64(tg_ctx *c, const TreeView &t, const Geom *d_geom, const uint2 *pairs, int64_t npairs,
-                         const uint2 *self_pairs, int64_t nself, const dbl4 *pf, const uint8_t *fs, bool masked,
-                         double *acc4);
+// (float64: xyzm holds the sorted coordinates and masses)
+tg_status launch_p2p_f64(tg_ctx *c, const TreeView &t, const uint2 *pairs, int64_t npairs, const uint2 *self_pairs,
+                         int64_t nself, const double *const xyzm[4], const int32_t *nslow, bool pot, double *acc4);
+tg_status launch_p2p_f64_dev(tg_ctx *c, const TreeView &t, const DevEval *de, const unsigned long long *walk_ctr,
+                             const uint2 *p2p, size_t cap_p2p, int cap_cells, const double *const xyzm[4],
+                             const int32_t *nslow, double *acc4, int stride, int scan_scratch = B_SCAN_TMP);
 
 // Kernels of tree.cu, also launched by the allocation-free sort in noalloc.cu.
 constexpr int kSortTileItems = 2048;     // items per radix-sort block (256 threads x 8)
