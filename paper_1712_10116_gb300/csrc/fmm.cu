@@ -991,9 +991,7 @@ static tg_status launch_m2l_t(tg_ctx *c, const TreeView &t, const M2LBlock *bloc
 static tg_status launch_m2l_t(tg_ctx *c, const TreeView &t, const M2LBlock *blocks, int64_t nblocks, const double *Ms,
                               double *L, int p, int nc, int ncp, bool masked, bool pot, const uint32_t *fpre)
 {
-    (void)fpre;   // the float64 contraction computes both classes for every pair
-    (void)pot;   // the float64 contraction always includes the potential term
-    return launch_m2l_f64(c, t, blocks, nblocks, Ms, L, p, nc, ncp, masked);
+    return launch_m2l_f64(c, t, blocks, nblocks, Ms, L, p, nc, ncp, masked, pot, fpre);
 }
 static tg_status launch_p2p_t(tg_ctx *c, const TreeView &t, const uint2 *pairs, int64_t npairs, const uint2 *self_pairs,
                               int64_t nself, const float4 *pf, const double *const xyzm[4], const int32_t *nslow,
@@ -1086,7 +1084,7 @@ static tg_status eval_typed(tg_ctx *c, int n, int ncell, const TreeView &t, cons
     const M2LBlock *blocks = static_cast<const M2LBlock *>(c->buf[B_M2L].p);
     const uint2 *p2p = static_cast<const uint2 *>(c->buf[B_P2P].p);
     uint32_t *fpre = nullptr;
-    if (masked && sizeof(T) == 4 && (st = fast_prefix(c, fs, n, &fpre, nullptr))) return st;
+    if (masked && p <= 6 && (st = fast_prefix(c, fs, n, &fpre, nullptr))) return st;   // the fixed-order M2L kernels
     if (n_blocks > 0 && (st = launch_m2l_t(c, t, blocks, n_blocks, Ms, L, p, nc, ncp, masked, want_pot, fpre))) return st;
     for (int l = 1; l < nlev; ++l) {
         const int lb = c->level_begin[l], le = c->level_begin[l + 1];
@@ -1404,16 +1402,16 @@ static tg_status fmm_eval_dev_t(tg_ctx *c, DevEval *de, const BatchCaps &cap, co
         zero_rows_dev<T><<<c->num_sms * 4, 256, 0, c->stream>>>(L, &de->rows, ncp);
     }
     cudaStreamWaitEvent(c->stream, c->ev_walk, 0);   // M2L reads the walk's blocks
-    if (sizeof(T) == 4) {
-        uint32_t *fpre = nullptr;
-        st = fast_prefix(c, fs2, cap.n, &fpre, de);
-        if (!st)
+    uint32_t *fpre = nullptr;
+    st = fast_prefix(c, fs2, cap.n, &fpre, de);
+    if (!st) {
+        if (sizeof(T) == 4)
             st = launch_m2l_f32_dev(c, t, de, d_geom, blocks, wctr + 1, (int64_t)cap.blocks,
                                     reinterpret_cast<const float *>(Ms), reinterpret_cast<float *>(L), p, ncp, cap.cells,
                                     cap.m2l_src, fpre);
-    } else {
-        st = launch_m2l_f64_dev(c, t, de, d_geom, blocks, wctr + 1, (int64_t)cap.blocks,
-                                reinterpret_cast<const double *>(Ms), reinterpret_cast<double *>(L), p, ncp);
+        else
+            st = launch_m2l_f64_dev(c, t, de, d_geom, blocks, wctr + 1, (int64_t)cap.blocks,
+                                    reinterpret_cast<const double *>(Ms), reinterpret_cast<double *>(L), p, ncp, fpre);
     }
     if (st) {
         cudaStreamWaitEvent(c->stream, c->ev_join, 0);   // no unjoined work on the side stream

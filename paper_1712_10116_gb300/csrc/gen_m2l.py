@@ -1,4 +1,4 @@
-"""Writes m2l_gen.cuh: straight-line float32 code for the mutual M2L at fixed order P.
+"""Writes m2l_gen.cuh: straight-line code for the mutual M2L at fixed order P, in float32 or float64 (T).
 
 For each P in 1..6 it emits
   m2l_dtensor_P(dx, dy, dz, soft2, D)   derivative tensor D^k(d), |k| <= P, of G = -(|d|^2 + soft2)^(-1/2)
@@ -43,18 +43,17 @@ def gen(P):
     idx = {v: i for i, v in enumerate(mi)}
     nc = len(mi)
     out = []
-    out.append(f"__device__ __forceinline__ void m2l_dtensor_{P}(float dx, float dy, float dz, float soft2, float (&D)[{nc}])")
+    out.append(f"template <class T> __device__ __forceinline__ void m2l_dtensor_{P}(T dx, T dy, T dz, T soft2, T (&D)[{nc}])")
     out.append("{")
-    out.append("    const float s2 = fmaf(dx, dx, fmaf(dy, dy, fmaf(dz, dz, soft2)));")
-    out.append("    float si = rsqrtf(s2);")
-    out.append("    si = si * fmaf(-0.5f * s2, si * si, 1.5f);   // one Newton step")
-    out.append("    const float si2 = si * si;")
-    out.append("    const float f0 = -si;")
+    out.append("    const T s2 = m2l_fma(dx, dx, m2l_fma(dy, dy, m2l_fma(dz, dz, soft2)));")
+    out.append("    const T si = m2l_rsqrt(s2);")
+    out.append("    const T si2 = si * si;")
+    out.append("    const T f0 = -si;")
     for m in range(1, P + 1):
-        out.append(f"    const float f{m} = {-(2 * m - 1)}.0f * f{m - 1} * si2;")
+        out.append(f"    const T f{m} = T({-(2 * m - 1)}) * f{m - 1} * si2;")
     # R^(m)_k named r_m_k ; r_m_0 = f_m
     for m in range(P + 1):
-        out.append(f"    const float r_{m}_0 = f{m};")
+        out.append(f"    const T r_{m}_0 = f{m};")
     axis_name = ["dx", "dy", "dz"]
     for k in range(1, nc):
         v = list(mi[k])
@@ -72,8 +71,8 @@ def gen(P):
         for m in range(P - o + 1):
             expr = f"{axis_name[a]} * r_{m + 1}_{km}"
             if kmm is not None:
-                expr = f"fmaf({float(ka - 1)}f, r_{m + 1}_{kmm}, {expr})"
-            out.append(f"    const float r_{m}_{k} = {expr};")
+                expr = f"m2l_fma(T({ka - 1}), r_{m + 1}_{kmm}, {expr})"
+            out.append(f"    const T r_{m}_{k} = {expr};")
     for k in range(nc):
         out.append(f"    D[{k}] = r_0_{k};")
     out.append("}")
@@ -82,11 +81,11 @@ def gen(P):
         suf = "" if pot else "_forces"
         first_n = 0 if pot else 1   # forces only: L^0 (the potential term) is left at zero
         # side A: L^n = sum_j (-1)^|j| rho^|j| Ms^j D^{n+j}
-        out.append(f"__device__ __forceinline__ void m2l_side_a{suf}_{P}(const float (&D)[{nc}], const float *__restrict__ Ms, float rho, float (&L)[{nc}])")
+        out.append(f"template <class T> __device__ __forceinline__ void m2l_side_a{suf}_{P}(const T (&D)[{nc}], const T *__restrict__ Ms, T rho, T (&L)[{nc}])")
         out.append("{")
         if not pot:
-            out.append("    L[0] = 0.0f;")
-        out.append("    float rp = 1.0f;")
+            out.append("    L[0] = T(0);")
+        out.append("    T rp = T(1);")
         prev_order = 0
         for j, (jx, jy, jz) in enumerate(mi):
             oj = jx + jy + jz
@@ -96,7 +95,7 @@ def gen(P):
                 out.append("    rp *= rho;")
                 prev_order = oj
             neg = (oj % 2) == 1
-            out.append(f"    {{ const float m = {'-' if neg else ''}__ldg(Ms + {j}) * rp;")
+            out.append(f"    {{ const T m = {'-' if neg else ''}__ldg(Ms + {j}) * rp;")
             for n, (nx, ny, nz) in enumerate(mi):
                 if n < first_n or nx + ny + nz + oj > P:
                     continue
@@ -104,20 +103,20 @@ def gen(P):
                 if j == 0:
                     out.append(f"      L[{n}] = D[{t}] * m;")
                 else:
-                    out.append(f"      L[{n}] = fmaf(D[{t}], m, L[{n}]);")
+                    out.append(f"      L[{n}] = m2l_fma(D[{t}], m, L[{n}]);")
             out.append("    }")
         out.append("}")
         out.append("")
         # side B: L^n = (-1)^|n| sum_j Ms^j D^{n+j}
-        out.append(f"__device__ __forceinline__ void m2l_side_b{suf}_{P}(const float (&D)[{nc}], const float *__restrict__ Ms, float (&L)[{nc}])")
+        out.append(f"template <class T> __device__ __forceinline__ void m2l_side_b{suf}_{P}(const T (&D)[{nc}], const T *__restrict__ Ms, T (&L)[{nc}])")
         out.append("{")
         if not pot:
-            out.append("    L[0] = 0.0f;")
+            out.append("    L[0] = T(0);")
         for j, (jx, jy, jz) in enumerate(mi):
             oj = jx + jy + jz
             if not pot and oj == P:
                 continue
-            out.append(f"    {{ const float m = __ldg(Ms + {j});")
+            out.append(f"    {{ const T m = __ldg(Ms + {j});")
             for n, (nx, ny, nz) in enumerate(mi):
                 on = nx + ny + nz
                 if n < first_n or on + oj > P:
@@ -127,7 +126,7 @@ def gen(P):
                 if j == 0:
                     out.append(f"      L[{n}] = {sign}D[{t}] * m;")
                 else:
-                    out.append(f"      L[{n}] = fmaf({sign}D[{t}], m, L[{n}]);")
+                    out.append(f"      L[{n}] = m2l_fma({sign}D[{t}], m, L[{n}]);")
             out.append("    }")
         out.append("}")
         out.append("")
@@ -145,17 +144,16 @@ def gen_h(P):
     didx = {v: i for i, v in enumerate(DS)}
     nh, nd = len(H), len(DS)
     out = []
-    out.append(f"__device__ __forceinline__ void m2l_dtensor_h_{P}(float dx, float dy, float dz, float (&D)[{nd}])")
+    out.append(f"template <class T> __device__ __forceinline__ void m2l_dtensor_h_{P}(T dx, T dy, T dz, T (&D)[{nd}])")
     out.append("{")
-    out.append("    const float s2 = fmaf(dx, dx, fmaf(dy, dy, dz * dz));")
-    out.append("    float si = rsqrtf(s2);")
-    out.append("    si = si * fmaf(-0.5f * s2, si * si, 1.5f);   // one Newton step")
-    out.append("    const float si2 = si * si;")
-    out.append("    const float f0 = -si;")
+    out.append("    const T s2 = m2l_fma(dx, dx, m2l_fma(dy, dy, dz * dz));")
+    out.append("    const T si = m2l_rsqrt(s2);")
+    out.append("    const T si2 = si * si;")
+    out.append("    const T f0 = -si;")
     for m in range(1, P + 1):
-        out.append(f"    const float f{m} = {-(2 * m - 1)}.0f * f{m - 1} * si2;")
+        out.append(f"    const T f{m} = T({-(2 * m - 1)}) * f{m - 1} * si2;")
     for m in range(P + 1):
-        out.append(f"    const float r_{m}_0 = f{m};")
+        out.append(f"    const T r_{m}_0 = f{m};")
     axis_name = ["dx", "dy", "dz"]
     # k_z = 0: the recurrence along x and y at every auxiliary level it feeds
     for k in range(1, nc):
@@ -176,8 +174,8 @@ def gen_h(P):
         for m in range(P - o + 1):
             expr = f"{axis_name[a]} * r_{m + 1}_{km}"
             if kmm is not None:
-                expr = f"fmaf({float(ka - 1)}f, r_{m + 1}_{kmm}, {expr})"
-            out.append(f"    const float r_{m}_{k} = {expr};")
+                expr = f"m2l_fma(T({ka - 1}), r_{m + 1}_{kmm}, {expr})"
+            out.append(f"    const T r_{m}_{k} = {expr};")
     for k, v in enumerate(DS):
         if v[2] == 0:
             out.append(f"    D[{k}] = r_0_{idx[v]};")
@@ -192,11 +190,11 @@ def gen_h(P):
     for pot in (True, False):
         suf = "" if pot else "_forces"
         first_n = 0 if pot else 1
-        out.append(f"__device__ __forceinline__ void m2l_side_a_h{suf}_{P}(const float (&D)[{nd}], const float *__restrict__ Mr, float rho, float (&L)[{nh}])")
+        out.append(f"template <class T> __device__ __forceinline__ void m2l_side_a_h{suf}_{P}(const T (&D)[{nd}], const T *__restrict__ Mr, T rho, T (&L)[{nh}])")
         out.append("{")
         if not pot:
-            out.append("    L[0] = 0.0f;")
-        out.append("    float rp = 1.0f;")
+            out.append("    L[0] = T(0);")
+        out.append("    T rp = T(1);")
         prev_order = 0
         for j, (jx, jy, jz) in enumerate(H):
             oj = jx + jy + jz
@@ -206,7 +204,7 @@ def gen_h(P):
                 out.append("    rp *= rho;")
                 prev_order = oj
             neg = (oj % 2) == 1
-            out.append(f"    {{ const float m = {'-' if neg else ''}__ldg(Mr + {j}) * rp;")
+            out.append(f"    {{ const T m = {'-' if neg else ''}__ldg(Mr + {j}) * rp;")
             for n, (nx, ny, nz) in enumerate(H):
                 if n < first_n or nx + ny + nz + oj > P:
                     continue
@@ -214,14 +212,14 @@ def gen_h(P):
                 if j == 0:
                     out.append(f"      L[{n}] = D[{t}] * m;")
                 else:
-                    out.append(f"      L[{n}] = fmaf(D[{t}], m, L[{n}]);")
+                    out.append(f"      L[{n}] = m2l_fma(D[{t}], m, L[{n}]);")
             out.append("    }")
         out.append("}")
         out.append("")
         # directed accumulation: L^n += sum_j (-1)^|j| rho^|j| Mr^j D^{n+j} (one target, one source)
-        out.append(f"__device__ __forceinline__ void m2l_acc_h{suf}_{P}(const float (&D)[{nd}], const float *__restrict__ Mr, float rho, float (&L)[{nh}])")
+        out.append(f"template <class T> __device__ __forceinline__ void m2l_acc_h{suf}_{P}(const T (&D)[{nd}], const T *__restrict__ Mr, T rho, T (&L)[{nh}])")
         out.append("{")
-        out.append("    float rp = 1.0f;")
+        out.append("    T rp = T(1);")
         prev_order = 0
         for j, (jx, jy, jz) in enumerate(H):
             oj = jx + jy + jz
@@ -231,24 +229,24 @@ def gen_h(P):
                 out.append("    rp *= rho;")
                 prev_order = oj
             neg = (oj % 2) == 1
-            out.append(f"    {{ const float m = {'-' if neg else ''}__ldg(Mr + {j}) * rp;")
+            out.append(f"    {{ const T m = {'-' if neg else ''}__ldg(Mr + {j}) * rp;")
             for n, (nx, ny, nz) in enumerate(H):
                 if n < first_n or nx + ny + nz + oj > P:
                     continue
                 t = didx[(nx + jx, ny + jy, nz + jz)]
-                out.append(f"      L[{n}] = fmaf(D[{t}], m, L[{n}]);")
+                out.append(f"      L[{n}] = m2l_fma(D[{t}], m, L[{n}]);")
             out.append("    }")
         out.append("}")
         out.append("")
-        out.append(f"__device__ __forceinline__ void m2l_side_b_h{suf}_{P}(const float (&D)[{nd}], const float *__restrict__ Mr, float (&L)[{nh}])")
+        out.append(f"template <class T> __device__ __forceinline__ void m2l_side_b_h{suf}_{P}(const T (&D)[{nd}], const T *__restrict__ Mr, T (&L)[{nh}])")
         out.append("{")
         if not pot:
-            out.append("    L[0] = 0.0f;")
+            out.append("    L[0] = T(0);")
         for j, (jx, jy, jz) in enumerate(H):
             oj = jx + jy + jz
             if not pot and oj == P:
                 continue
-            out.append(f"    {{ const float m = __ldg(Mr + {j});")
+            out.append(f"    {{ const T m = __ldg(Mr + {j});")
             for n, (nx, ny, nz) in enumerate(H):
                 on = nx + ny + nz
                 if n < first_n or on + oj > P:
@@ -258,15 +256,15 @@ def gen_h(P):
                 if j == 0:
                     out.append(f"      L[{n}] = {sign}D[{t}] * m;")
                 else:
-                    out.append(f"      L[{n}] = fmaf({sign}D[{t}], m, L[{n}]);")
+                    out.append(f"      L[{n}] = m2l_fma({sign}D[{t}], m, L[{n}]);")
             out.append("    }")
         out.append("}")
         out.append("")
     # per cell: fold the j_z >= 2 moments down (highest j_z first), keep the j_z <= 1 ones
-    out.append(f"__device__ __forceinline__ void m2l_reduce_moments_h_{P}(const float *__restrict__ Ms, float *__restrict__ Mr)")
+    out.append(f"template <class T> __device__ __forceinline__ void m2l_reduce_moments_h_{P}(const T *__restrict__ Ms, T *__restrict__ Mr)")
     out.append("{")
     for k in range(nc):
-        out.append(f"    float v{k} = Ms[{k}];")
+        out.append(f"    T v{k} = Ms[{k}];")
     for jz in range(P, 1, -1):
         for k, v in enumerate(mi):
             if v[2] != jz:
@@ -280,13 +278,13 @@ def gen_h(P):
     out.append("}")
     out.append("")
     # per cell: the locals with n_z >= 2 from the harmonic relation (their two partners come earlier)
-    out.append(f"__device__ __forceinline__ void m2l_complete_locals_h_{P}(const float *__restrict__ Lr, float *__restrict__ L)")
+    out.append(f"template <class T> __device__ __forceinline__ void m2l_complete_locals_h_{P}(const T *__restrict__ Lr, T *__restrict__ L)")
     out.append("{")
     for k, v in enumerate(mi):
         if v[2] <= 1:
-            out.append(f"    const float v{k} = Lr[{hidx[v]}];")
+            out.append(f"    const T v{k} = Lr[{hidx[v]}];")
         else:
-            out.append(f"    const float v{k} = -v{idx[(v[0] + 2, v[1], v[2] - 2)]} - v{idx[(v[0], v[1] + 2, v[2] - 2)]};")
+            out.append(f"    const T v{k} = -v{idx[(v[0] + 2, v[1], v[2] - 2)]} - v{idx[(v[0], v[1] + 2, v[2] - 2)]};")
         out.append(f"    L[{k}] = v{k};")
     out.append("}")
     out.append("")
@@ -294,8 +292,19 @@ def gen_h(P):
 
 
 def main():
-    print("// Generated by gen_m2l.py -- fixed-order float32 M2L building blocks (do not edit).")
+    print("// Generated by gen_m2l.py -- fixed-order M2L building blocks (do not edit).")
     print("#pragma once")
+    print()
+    print("__device__ __forceinline__ float m2l_fma(float a, float b, float c) { return fmaf(a, b, c); }")
+    print("__device__ __forceinline__ float m2l_rsqrt(float s)")
+    print("{")
+    print("    const float y = rsqrtf(s);")
+    print("    return y * fmaf(-0.5f * s, y * y, 1.5f);   // one Newton step")
+    print("}")
+    print("#ifdef __CUDACC__")
+    print("__device__ __forceinline__ double m2l_fma(double a, double b, double c) { return fma(a, b, c); }")
+    print("__device__ __forceinline__ double m2l_rsqrt(double s) { return rsqrt(s); }")
+    print("#endif")
     print()
     for P in range(1, PMAX_GEN + 1):
         print(gen(P))
@@ -304,11 +313,11 @@ def main():
         nc = len(multi_indices(P))
         print(f"template <> struct M2LGen<{P}> {{")
         print(f"    static constexpr int NC = {nc};")
-        print(f"    static __device__ __forceinline__ void dtensor(float dx, float dy, float dz, float s, float (&D)[{nc}]) {{ m2l_dtensor_{P}(dx, dy, dz, s, D); }}")
-        print(f"    static __device__ __forceinline__ void side_a(const float (&D)[{nc}], const float *Ms, float rho, float (&L)[{nc}]) {{ m2l_side_a_{P}(D, Ms, rho, L); }}")
-        print(f"    static __device__ __forceinline__ void side_b(const float (&D)[{nc}], const float *Ms, float (&L)[{nc}]) {{ m2l_side_b_{P}(D, Ms, L); }}")
-        print(f"    static __device__ __forceinline__ void side_a_forces(const float (&D)[{nc}], const float *Ms, float rho, float (&L)[{nc}]) {{ m2l_side_a_forces_{P}(D, Ms, rho, L); }}")
-        print(f"    static __device__ __forceinline__ void side_b_forces(const float (&D)[{nc}], const float *Ms, float (&L)[{nc}]) {{ m2l_side_b_forces_{P}(D, Ms, L); }}")
+        print(f"    template <class T> static __device__ __forceinline__ void dtensor(T dx, T dy, T dz, T s, T (&D)[{nc}]) {{ m2l_dtensor_{P}(dx, dy, dz, s, D); }}")
+        print(f"    template <class T> static __device__ __forceinline__ void side_a(const T (&D)[{nc}], const T *Ms, T rho, T (&L)[{nc}]) {{ m2l_side_a_{P}(D, Ms, rho, L); }}")
+        print(f"    template <class T> static __device__ __forceinline__ void side_b(const T (&D)[{nc}], const T *Ms, T (&L)[{nc}]) {{ m2l_side_b_{P}(D, Ms, L); }}")
+        print(f"    template <class T> static __device__ __forceinline__ void side_a_forces(const T (&D)[{nc}], const T *Ms, T rho, T (&L)[{nc}]) {{ m2l_side_a_forces_{P}(D, Ms, rho, L); }}")
+        print(f"    template <class T> static __device__ __forceinline__ void side_b_forces(const T (&D)[{nc}], const T *Ms, T (&L)[{nc}]) {{ m2l_side_b_forces_{P}(D, Ms, L); }}")
         print("};")
     for P in range(1, PMAX_GEN + 1):
         print(gen_h(P))
@@ -320,15 +329,15 @@ def main():
         print(f"template <> struct M2LGenH<{P}> {{")
         print(f"    static constexpr int NC = {nh};")
         print(f"    static constexpr int ND = {nd};")
-        print(f"    static __device__ __forceinline__ void dtensor(float dx, float dy, float dz, float (&D)[{nd}]) {{ m2l_dtensor_h_{P}(dx, dy, dz, D); }}")
-        print(f"    static __device__ __forceinline__ void side_a(const float (&D)[{nd}], const float *Mr, float rho, float (&L)[{nh}]) {{ m2l_side_a_h_{P}(D, Mr, rho, L); }}")
-        print(f"    static __device__ __forceinline__ void side_b(const float (&D)[{nd}], const float *Mr, float (&L)[{nh}]) {{ m2l_side_b_h_{P}(D, Mr, L); }}")
-        print(f"    static __device__ __forceinline__ void side_a_forces(const float (&D)[{nd}], const float *Mr, float rho, float (&L)[{nh}]) {{ m2l_side_a_h_forces_{P}(D, Mr, rho, L); }}")
-        print(f"    static __device__ __forceinline__ void side_b_forces(const float (&D)[{nd}], const float *Mr, float (&L)[{nh}]) {{ m2l_side_b_h_forces_{P}(D, Mr, L); }}")
-        print(f"    static __device__ __forceinline__ void acc(const float (&D)[{nd}], const float *Mr, float rho, float (&L)[{nh}]) {{ m2l_acc_h_{P}(D, Mr, rho, L); }}")
-        print(f"    static __device__ __forceinline__ void acc_forces(const float (&D)[{nd}], const float *Mr, float rho, float (&L)[{nh}]) {{ m2l_acc_h_forces_{P}(D, Mr, rho, L); }}")
-        print(f"    static __device__ __forceinline__ void reduce_moments(const float *Ms, float *Mr) {{ m2l_reduce_moments_h_{P}(Ms, Mr); }}")
-        print(f"    static __device__ __forceinline__ void complete_locals(const float *Lr, float *L) {{ m2l_complete_locals_h_{P}(Lr, L); }}")
+        print(f"    template <class T> static __device__ __forceinline__ void dtensor(T dx, T dy, T dz, T (&D)[{nd}]) {{ m2l_dtensor_h_{P}(dx, dy, dz, D); }}")
+        print(f"    template <class T> static __device__ __forceinline__ void side_a(const T (&D)[{nd}], const T *Mr, T rho, T (&L)[{nh}]) {{ m2l_side_a_h_{P}(D, Mr, rho, L); }}")
+        print(f"    template <class T> static __device__ __forceinline__ void side_b(const T (&D)[{nd}], const T *Mr, T (&L)[{nh}]) {{ m2l_side_b_h_{P}(D, Mr, L); }}")
+        print(f"    template <class T> static __device__ __forceinline__ void side_a_forces(const T (&D)[{nd}], const T *Mr, T rho, T (&L)[{nh}]) {{ m2l_side_a_h_forces_{P}(D, Mr, rho, L); }}")
+        print(f"    template <class T> static __device__ __forceinline__ void side_b_forces(const T (&D)[{nd}], const T *Mr, T (&L)[{nh}]) {{ m2l_side_b_h_forces_{P}(D, Mr, L); }}")
+        print(f"    template <class T> static __device__ __forceinline__ void acc(const T (&D)[{nd}], const T *Mr, T rho, T (&L)[{nh}]) {{ m2l_acc_h_{P}(D, Mr, rho, L); }}")
+        print(f"    template <class T> static __device__ __forceinline__ void acc_forces(const T (&D)[{nd}], const T *Mr, T rho, T (&L)[{nh}]) {{ m2l_acc_h_forces_{P}(D, Mr, rho, L); }}")
+        print(f"    template <class T> static __device__ __forceinline__ void reduce_moments(const T *Ms, T *Mr) {{ m2l_reduce_moments_h_{P}(Ms, Mr); }}")
+        print(f"    template <class T> static __device__ __forceinline__ void complete_locals(const T *Lr, T *L) {{ m2l_complete_locals_h_{P}(Lr, L); }}")
         print("};")
 
 

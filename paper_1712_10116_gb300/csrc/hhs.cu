@@ -704,7 +704,7 @@ static tg_status hold_presize(tg_ctx *c, const Sched &s, const BatchCaps &cap, c
         {B_C_COUNT, 4ull * C}, {B_C_CHILD, 4ull * C}, {B_C_PARENT, 4ull * C}, {B_C_NCHILD, 1ull * C},
         {B_C_TMP0, 4ull * C}, {B_C_TMP1, 4ull * C},
         {B_MOM, tsz * rows * ncp}, {B_MOMF, tsz * rows * ncp}, {B_MOM01, 8 * rows * 4}, {B_LOC, tsz * rows * ncp},
-        {B_ACC, 32ull * n}, {B_MOMH, 4 * rows * ncpr}, {B_LOCH, 4 * rows * ncpr},
+        {B_ACC, 32ull * n}, {B_MOMH, tsz * rows * ncpr}, {B_LOCH, tsz * rows * ncpr},
         {B_FRONT0, 8 * cap.front}, {B_FRONT1, 8 * cap.front}, {B_M2L, 16 * cap.blocks}, {B_P2P, 8 * cap.p2p},
         {B_WALK_CNT, 8 * (8 + 24 + 1)},
         {B_OWN_CNT, 4ull * (C + 2)}, {B_OWN_FILL, 4ull * (C + 2)}, {B_OWN_OFF, 4ull * C},

@@ -1,6 +1,6 @@
-// m2l.cu -- launchers of the mutual M2L kernels (Sec. 2.1): float32 fixed-order block kernels for
-// p <= 6 (harmonic contraction set for the Wendland kernel, full set for Plummer softening), the
-// generic kernel otherwise and in float64 up to the table order, high_order.cu above it.  Its own translation unit, so that the large
+// m2l.cu -- launchers of the mutual M2L kernels (Sec. 2.1): fixed-order kernels for p <= 6
+// (float32 by block, float64 by pair; harmonic contraction set for the Wendland kernel, full set for Plummer
+// softening), the generic kernel up to the table order, high_order.cu above it.  Its own translation unit, so that the large
 // generated contractions compile in parallel with the rest.
 #include <algorithm>
 
@@ -8,6 +8,14 @@
 #include "m2l_sym.cuh"
 
 namespace tg {
+
+// zero rows[0] rows of `width` values (device row count)
+template <class T>
+__global__ void zero_rows(T *p, const int *rows, int width)
+{
+    const int64_t n = (int64_t)*rows * width;
+    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) p[i] = T(0);
+}
 
 // zero n (+ extra) words, n from the device when dn is given (dn[0] + extra)
 __global__ void zero_u32(uint32_t *p, int n, const int *dn, int extra)
@@ -98,10 +106,10 @@ static tg_status m2l_f32_harmonic(tg_ctx *c, const TreeView &t, const M2LBlock *
             return st;
         if ((st = m2l_lists(c, t, blocks, nblocks, ncell, cnt, off, fill, src, cap, nullptr, nullptr))) return st;
         ProfScope ps_(c, TG_K_M2L);
-        m2l_reduce_moments_h<P><<<grid_for(rows, 128), 128, 0, c->stream>>>(rows, Ms, ncp, Mr, ncpr, nullptr);
+        m2l_reduce_moments_h<P, float><<<grid_for(rows, 128), 128, 0, c->stream>>>(rows, Ms, ncp, Mr, ncpr, nullptr);
         cudaMemsetAsync(Lr, 0, sizeof(float) * (size_t)rows * ncpr, c->stream);
         m2l_directed_launch<P>(c, t, off, cnt, src, cap, Mr, Lr, ncpr, masked, pot, nullptr);
-        m2l_complete_locals_h<P><<<grid_for(rows, 128), 128, 0, c->stream>>>(rows, Lr, ncpr, L, ncp, nullptr);
+        m2l_complete_locals_h<P, float><<<grid_for(rows, 128), 128, 0, c->stream>>>(rows, Lr, ncpr, L, ncp, nullptr);
         return cuda_check(c, cudaGetLastError(), "m2l launch (directed)");
     }
     constexpr int NH = M2LGenH<P>::NC;
@@ -115,7 +123,7 @@ static tg_status m2l_f32_harmonic(tg_ctx *c, const TreeView &t, const M2LBlock *
         return st;
     if ((st = m2l_partition_blocks(c, blocks, nblocks, nullptr, &part, &pcnt))) return st;
     ProfScope ps_(c, TG_K_M2L);
-    m2l_reduce_moments_h<P><<<grid_for(rows, 128), 128, 0, c->stream>>>(rows, Ms, ncp, Mr, ncpr, nullptr);
+    m2l_reduce_moments_h<P, float><<<grid_for(rows, 128), 128, 0, c->stream>>>(rows, Ms, ncp, Mr, ncpr, nullptr);
     cudaMemsetAsync(Lr, 0, sizeof(float) * (size_t)rows * ncpr, c->stream);
     using G = M2LHarm<P>;
 #define TG_M2L_H(MK, PT)                                                                                          \
@@ -131,7 +139,7 @@ static tg_status m2l_f32_harmonic(tg_ctx *c, const TreeView &t, const M2LBlock *
         else TG_M2L_H(false, false);
     }
 #undef TG_M2L_H
-    m2l_complete_locals_h<P><<<grid_for(rows, 128), 128, 0, c->stream>>>(rows, Lr, ncpr, L, ncp, nullptr);
+    m2l_complete_locals_h<P, float><<<grid_for(rows, 128), 128, 0, c->stream>>>(rows, Lr, ncpr, L, ncp, nullptr);
     return cuda_check(c, cudaGetLastError(), "m2l launch");
 }
 
@@ -217,10 +225,10 @@ static tg_status m2l_f32_dev_p(tg_ctx *c, const TreeView &t, const DevEval *de, 
             return st;
         ProfScope ps_(c, TG_K_M2L);
         m2l_list_check<<<1, 1, 0, c->stream>>>(off, cnt, const_cast<DevEval *>(de), cap_src);
-        m2l_reduce_moments_h<P><<<g, 128, 0, c->stream>>>(rows_cap, Ms, ncp, Mr, ncpr, &de->rows);
-        zero_rows_f32<<<c->num_sms * 4, 256, 0, c->stream>>>(Lr, &de->rows, ncpr);
+        m2l_reduce_moments_h<P, float><<<g, 128, 0, c->stream>>>(rows_cap, Ms, ncp, Mr, ncpr, &de->rows);
+        zero_rows<float><<<c->num_sms * 4, 256, 0, c->stream>>>(Lr, &de->rows, ncpr);
         m2l_directed_launch<P>(c, t, off, cnt, src, cap_src, Mr, Lr, ncpr, true, false, de);
-        m2l_complete_locals_h<P><<<g, 128, 0, c->stream>>>(rows_cap, Lr, ncpr, L, ncp, &de->rows);
+        m2l_complete_locals_h<P, float><<<g, 128, 0, c->stream>>>(rows_cap, Lr, ncpr, L, ncp, &de->rows);
         return TG_OK;
     }
     M2LBlock *part;
@@ -231,13 +239,13 @@ static tg_status m2l_f32_dev_p(tg_ctx *c, const TreeView &t, const DevEval *de, 
     if (!plummer) {
         // harmonic set: fold, contract (the launch for the other class count returns at once), complete
         using G = M2LHarm<P>;
-        m2l_reduce_moments_h<P><<<g, 128, 0, c->stream>>>(rows_cap, Ms, ncp, Mr, ncpr, &de->rows);
-        zero_rows_f32<<<c->num_sms * 4, 256, 0, c->stream>>>(Lr, &de->rows, ncpr);
+        m2l_reduce_moments_h<P, float><<<g, 128, 0, c->stream>>>(rows_cap, Ms, ncp, Mr, ncpr, &de->rows);
+        zero_rows<float><<<c->num_sms * 4, 256, 0, c->stream>>>(Lr, &de->rows, ncpr);
         m2l_blocks_f32<G, true, false><<<grid, 128, 0, c->stream>>>(t, part, cap_blocks, pcnt, Mr, Lr, ncpr, 0.f, 0, de,
                                                                     gp, c->prm.eps, fpre, c->d_counters + 11);
         m2l_blocks_f32<G, false, false><<<grid, 128, 0, c->stream>>>(t, part, cap_blocks, pcnt, Mr, Lr, ncpr, 0.f, 0, de,
                                                                      gp, c->prm.eps, fpre, c->d_counters + 11);
-        m2l_complete_locals_h<P><<<g, 128, 0, c->stream>>>(rows_cap, Lr, ncpr, L, ncp, &de->rows);
+        m2l_complete_locals_h<P, float><<<g, 128, 0, c->stream>>>(rows_cap, Lr, ncpr, L, ncp, &de->rows);
     } else {
         using G = M2LFull<P>;
         m2l_blocks_f32<G, true, false><<<grid, 128, 0, c->stream>>>(t, part, cap_blocks, pcnt, Ms, L, ncp, 0.f, 1, de,
@@ -274,24 +282,82 @@ tg_status launch_m2l_f32_dev(tg_ctx *c, const TreeView &t, const DevEval *de, co
     return cuda_check(c, cudaGetLastError(), "m2l launch (device sizes)");
 }
 
+// float64, P <= 6: the harmonic set (Wendland) folds the moments, contracts into Lr and completes L; with de every
+// count is on the device (nb and rows are then capacities, and the launch for the other class count returns).
+template <int P>
+static tg_status m2l_f64_p(tg_ctx *c, const TreeView &t, const M2LBlock *blocks, int64_t nb, const double *Ms, double *L,
+                           int ncp, bool masked, bool pot, const uint32_t *fpre, const DevEval *de, const Geom *gp,
+                           const unsigned long long *dnb)
+{
+    const bool plummer = c->prm.kernel == TG_KERNEL_PLUMMER;
+    const double eoL = de ? 0.0 : ldexp(c->prm.eps, -c->walk_log2L);
+    const int grid = c->num_sms * 4;
+    constexpr int NH = M2LGenH<P>::NC;
+    const int ncpr = (NH + 3) & ~3;
+    const int64_t rows = (int64_t)t.ncell * 2;
+    const int *drows = de ? &de->rows : nullptr;
+    double *Mr = nullptr, *Lr = nullptr;
+    tg_status st;
+    if (!plummer && ((st = ensure_t(c, B_MOMH, (size_t)rows * ncpr, &Mr)) || (st = ensure_t(c, B_LOCH, (size_t)rows * ncpr, &Lr))))
+        return st;
+    ProfScope ps_(c, TG_K_M2L);
+    if (!plummer) {
+        m2l_reduce_moments_h<P, double><<<grid_for(rows, 128), 128, 0, c->stream>>>(rows, Ms, ncp, Mr, ncpr, drows);
+        if (de) zero_rows<double><<<c->num_sms * 4, 256, 0, c->stream>>>(Lr, drows, ncpr);
+        else cudaMemsetAsync(Lr, 0, sizeof(double) * (size_t)rows * ncpr, c->stream);
+    }
+#define TG_M2L64_(G, MK, PT, MS, LL, NCP)                                                                          \
+    m2l_pairs_f64<G, MK, PT><<<grid, 128, 0, c->stream>>>(t, blocks, nb, dnb, MS, LL, NCP, eoL, plummer, de, gp,    \
+                                                          c->prm.eps, fpre)
+#define TG_M2L64(MK, PT)                                                                                           \
+    do {                                                                                                           \
+        if (plummer) TG_M2L64_(M2LFull<P>, MK, PT, Ms, L, ncp);                                                    \
+        else TG_M2L64_(M2LHarm<P>, MK, PT, Mr, Lr, ncpr);                                                          \
+    } while (0)
+    if (de) {
+        TG_M2L64(true, false);
+        TG_M2L64(false, false);
+    } else if (masked) {
+        if (pot) TG_M2L64(true, true);
+        else TG_M2L64(true, false);
+    } else {
+        if (pot) TG_M2L64(false, true);
+        else TG_M2L64(false, false);
+    }
+#undef TG_M2L64
+#undef TG_M2L64_
+    if (!plummer)
+        m2l_complete_locals_h<P, double><<<grid_for(rows, 128), 128, 0, c->stream>>>(rows, Lr, ncpr, L, ncp, drows);
+    return cuda_check(c, cudaGetLastError(), "m2l launch (float64)");
+}
+
+static tg_status m2l_f64_any(tg_ctx *c, const TreeView &t, const M2LBlock *blocks, int64_t nb, const double *Ms, double *L,
+                             int p, int ncp, bool masked, bool pot, const uint32_t *fpre, const DevEval *de,
+                             const Geom *gp, const unsigned long long *dnb)
+{
+    switch (p) {
+    case 1: return m2l_f64_p<1>(c, t, blocks, nb, Ms, L, ncp, masked, pot, fpre, de, gp, dnb);
+    case 2: return m2l_f64_p<2>(c, t, blocks, nb, Ms, L, ncp, masked, pot, fpre, de, gp, dnb);
+    case 3: return m2l_f64_p<3>(c, t, blocks, nb, Ms, L, ncp, masked, pot, fpre, de, gp, dnb);
+    case 4: return m2l_f64_p<4>(c, t, blocks, nb, Ms, L, ncp, masked, pot, fpre, de, gp, dnb);
+    case 5: return m2l_f64_p<5>(c, t, blocks, nb, Ms, L, ncp, masked, pot, fpre, de, gp, dnb);
+    default: return m2l_f64_p<6>(c, t, blocks, nb, Ms, L, ncp, masked, pot, fpre, de, gp, dnb);
+    }
+}
+
 tg_status launch_m2l_f64_dev(tg_ctx *c, const TreeView &t, const DevEval *de, const Geom *gp, const M2LBlock *blocks,
                              const unsigned long long *dnb, int64_t cap_blocks, const double *Ms, double *L, int p,
-                             int ncp)
+                             int ncp, const uint32_t *fpre)
 {
-    const int plummer = c->prm.kernel == TG_KERNEL_PLUMMER;
-    const int grid = c->num_sms * 16, nc = ncoef(p);
-    ProfScope ps_(c, TG_K_M2L);
-    m2l_blocks_generic<double, true><<<grid, 128, 0, c->stream>>>(t, blocks, cap_blocks, Ms, L, p, nc, ncp, 0.0, plummer,
-                                                                  dnb, de, gp, c->prm.eps);
-    m2l_blocks_generic<double, false><<<grid, 128, 0, c->stream>>>(t, blocks, cap_blocks, Ms, L, p, nc, ncp, 0.0, plummer,
-                                                                   dnb, de, gp, c->prm.eps);
-    return cuda_check(c, cudaGetLastError(), "m2l launch (device sizes, float64)");
+    if (p < 1 || p > 6) return set_err(c, TG_ERR_ARG, "batched M2L needs 1 <= p <= 6");
+    return m2l_f64_any(c, t, blocks, cap_blocks, Ms, L, p, ncp, true, false, fpre, de, gp, dnb);
 }
 
 tg_status launch_m2l_f64(tg_ctx *c, const TreeView &t, const M2LBlock *blocks, int64_t nblocks, const double *Ms,
-                         double *L, int p, int nc, int ncp, bool masked)
+                         double *L, int p, int nc, int ncp, bool masked, bool pot, const uint32_t *fpre)
 {
     if (p > TG_PMAX) return launch_m2l_hi<double>(c, t, blocks, nblocks, Ms, L, p, nc, ncp, masked, true);
+    if (p <= 6) return m2l_f64_any(c, t, blocks, nblocks, Ms, L, p, ncp, masked, pot, fpre, nullptr, nullptr, nullptr);
     const int plummer = c->prm.kernel == TG_KERNEL_PLUMMER;
     const double eoL = ldexp(c->prm.eps, -c->walk_log2L);
     const int grid = grid_for(nblocks * 32, 128, c->num_sms * 16);

@@ -1,110 +1,119 @@
-// Generated by gen_m2l.py -- fixed-order float32 M2L building blocks (do not edit).
+// Generated by gen_m2l.py -- fixed-order M2L building blocks (do not edit).
 #pragma once
 
-__device__ __forceinline__ void m2l_dtensor_1(float dx, float dy, float dz, float soft2, float (&D)[4])
+__device__ __forceinline__ float m2l_fma(float a, float b, float c) { return fmaf(a, b, c); }
+__device__ __forceinline__ float m2l_rsqrt(float s)
 {
-    const float s2 = fmaf(dx, dx, fmaf(dy, dy, fmaf(dz, dz, soft2)));
-    float si = rsqrtf(s2);
-    si = si * fmaf(-0.5f * s2, si * si, 1.5f);   // one Newton step
-    const float si2 = si * si;
-    const float f0 = -si;
-    const float f1 = -1.0f * f0 * si2;
-    const float r_0_0 = f0;
-    const float r_1_0 = f1;
-    const float r_0_1 = dx * r_1_0;
-    const float r_0_2 = dy * r_1_0;
-    const float r_0_3 = dz * r_1_0;
+    const float y = rsqrtf(s);
+    return y * fmaf(-0.5f * s, y * y, 1.5f);   // one Newton step
+}
+#ifdef __CUDACC__
+__device__ __forceinline__ double m2l_fma(double a, double b, double c) { return fma(a, b, c); }
+__device__ __forceinline__ double m2l_rsqrt(double s) { return rsqrt(s); }
+#endif
+
+template <class T> __device__ __forceinline__ void m2l_dtensor_1(T dx, T dy, T dz, T soft2, T (&D)[4])
+{
+    const T s2 = m2l_fma(dx, dx, m2l_fma(dy, dy, m2l_fma(dz, dz, soft2)));
+    const T si = m2l_rsqrt(s2);
+    const T si2 = si * si;
+    const T f0 = -si;
+    const T f1 = T(-1) * f0 * si2;
+    const T r_0_0 = f0;
+    const T r_1_0 = f1;
+    const T r_0_1 = dx * r_1_0;
+    const T r_0_2 = dy * r_1_0;
+    const T r_0_3 = dz * r_1_0;
     D[0] = r_0_0;
     D[1] = r_0_1;
     D[2] = r_0_2;
     D[3] = r_0_3;
 }
 
-__device__ __forceinline__ void m2l_side_a_1(const float (&D)[4], const float *__restrict__ Ms, float rho, float (&L)[4])
+template <class T> __device__ __forceinline__ void m2l_side_a_1(const T (&D)[4], const T *__restrict__ Ms, T rho, T (&L)[4])
 {
-    float rp = 1.0f;
-    { const float m = __ldg(Ms + 0) * rp;
+    T rp = T(1);
+    { const T m = __ldg(Ms + 0) * rp;
       L[0] = D[0] * m;
       L[1] = D[1] * m;
       L[2] = D[2] * m;
       L[3] = D[3] * m;
     }
     rp *= rho;
-    { const float m = -__ldg(Ms + 1) * rp;
-      L[0] = fmaf(D[1], m, L[0]);
+    { const T m = -__ldg(Ms + 1) * rp;
+      L[0] = m2l_fma(D[1], m, L[0]);
     }
-    { const float m = -__ldg(Ms + 2) * rp;
-      L[0] = fmaf(D[2], m, L[0]);
+    { const T m = -__ldg(Ms + 2) * rp;
+      L[0] = m2l_fma(D[2], m, L[0]);
     }
-    { const float m = -__ldg(Ms + 3) * rp;
-      L[0] = fmaf(D[3], m, L[0]);
+    { const T m = -__ldg(Ms + 3) * rp;
+      L[0] = m2l_fma(D[3], m, L[0]);
     }
 }
 
-__device__ __forceinline__ void m2l_side_b_1(const float (&D)[4], const float *__restrict__ Ms, float (&L)[4])
+template <class T> __device__ __forceinline__ void m2l_side_b_1(const T (&D)[4], const T *__restrict__ Ms, T (&L)[4])
 {
-    { const float m = __ldg(Ms + 0);
+    { const T m = __ldg(Ms + 0);
       L[0] = D[0] * m;
       L[1] = -D[1] * m;
       L[2] = -D[2] * m;
       L[3] = -D[3] * m;
     }
-    { const float m = __ldg(Ms + 1);
-      L[0] = fmaf(D[1], m, L[0]);
+    { const T m = __ldg(Ms + 1);
+      L[0] = m2l_fma(D[1], m, L[0]);
     }
-    { const float m = __ldg(Ms + 2);
-      L[0] = fmaf(D[2], m, L[0]);
+    { const T m = __ldg(Ms + 2);
+      L[0] = m2l_fma(D[2], m, L[0]);
     }
-    { const float m = __ldg(Ms + 3);
-      L[0] = fmaf(D[3], m, L[0]);
+    { const T m = __ldg(Ms + 3);
+      L[0] = m2l_fma(D[3], m, L[0]);
     }
 }
 
-__device__ __forceinline__ void m2l_side_a_forces_1(const float (&D)[4], const float *__restrict__ Ms, float rho, float (&L)[4])
+template <class T> __device__ __forceinline__ void m2l_side_a_forces_1(const T (&D)[4], const T *__restrict__ Ms, T rho, T (&L)[4])
 {
-    L[0] = 0.0f;
-    float rp = 1.0f;
-    { const float m = __ldg(Ms + 0) * rp;
+    L[0] = T(0);
+    T rp = T(1);
+    { const T m = __ldg(Ms + 0) * rp;
       L[1] = D[1] * m;
       L[2] = D[2] * m;
       L[3] = D[3] * m;
     }
 }
 
-__device__ __forceinline__ void m2l_side_b_forces_1(const float (&D)[4], const float *__restrict__ Ms, float (&L)[4])
+template <class T> __device__ __forceinline__ void m2l_side_b_forces_1(const T (&D)[4], const T *__restrict__ Ms, T (&L)[4])
 {
-    L[0] = 0.0f;
-    { const float m = __ldg(Ms + 0);
+    L[0] = T(0);
+    { const T m = __ldg(Ms + 0);
       L[1] = -D[1] * m;
       L[2] = -D[2] * m;
       L[3] = -D[3] * m;
     }
 }
 
-__device__ __forceinline__ void m2l_dtensor_2(float dx, float dy, float dz, float soft2, float (&D)[10])
+template <class T> __device__ __forceinline__ void m2l_dtensor_2(T dx, T dy, T dz, T soft2, T (&D)[10])
 {
-    const float s2 = fmaf(dx, dx, fmaf(dy, dy, fmaf(dz, dz, soft2)));
-    float si = rsqrtf(s2);
-    si = si * fmaf(-0.5f * s2, si * si, 1.5f);   // one Newton step
-    const float si2 = si * si;
-    const float f0 = -si;
-    const float f1 = -1.0f * f0 * si2;
-    const float f2 = -3.0f * f1 * si2;
-    const float r_0_0 = f0;
-    const float r_1_0 = f1;
-    const float r_2_0 = f2;
-    const float r_0_1 = dx * r_1_0;
-    const float r_1_1 = dx * r_2_0;
-    const float r_0_2 = dy * r_1_0;
-    const float r_1_2 = dy * r_2_0;
-    const float r_0_3 = dz * r_1_0;
-    const float r_1_3 = dz * r_2_0;
-    const float r_0_4 = fmaf(1.0f, r_1_0, dx * r_1_1);
-    const float r_0_5 = dx * r_1_2;
-    const float r_0_6 = dx * r_1_3;
-    const float r_0_7 = fmaf(1.0f, r_1_0, dy * r_1_2);
-    const float r_0_8 = dy * r_1_3;
-    const float r_0_9 = fmaf(1.0f, r_1_0, dz * r_1_3);
+    const T s2 = m2l_fma(dx, dx, m2l_fma(dy, dy, m2l_fma(dz, dz, soft2)));
+    const T si = m2l_rsqrt(s2);
+    const T si2 = si * si;
+    const T f0 = -si;
+    const T f1 = T(-1) * f0 * si2;
+    const T f2 = T(-3) * f1 * si2;
+    const T r_0_0 = f0;
+    const T r_1_0 = f1;
+    const T r_2_0 = f2;
+    const T r_0_1 = dx * r_1_0;
+    const T r_1_1 = dx * r_2_0;
+    const T r_0_2 = dy * r_1_0;
+    const T r_1_2 = dy * r_2_0;
+    const T r_0_3 = dz * r_1_0;
+    const T r_1_3 = dz * r_2_0;
+    const T r_0_4 = m2l_fma(T(1), r_1_0, dx * r_1_1);
+    const T r_0_5 = dx * r_1_2;
+    const T r_0_6 = dx * r_1_3;
+    const T r_0_7 = m2l_fma(T(1), r_1_0, dy * r_1_2);
+    const T r_0_8 = dy * r_1_3;
+    const T r_0_9 = m2l_fma(T(1), r_1_0, dz * r_1_3);
     D[0] = r_0_0;
     D[1] = r_0_1;
     D[2] = r_0_2;
@@ -117,10 +126,10 @@ __device__ __forceinline__ void m2l_dtensor_2(float dx, float dy, float dz, floa
     D[9] = r_0_9;
 }
 
-__device__ __forceinline__ void m2l_side_a_2(const float (&D)[10], const float *__restrict__ Ms, float rho, float (&L)[10])
+template <class T> __device__ __forceinline__ void m2l_side_a_2(const T (&D)[10], const T *__restrict__ Ms, T rho, T (&L)[10])
 {
-    float rp = 1.0f;
-    { const float m = __ldg(Ms + 0) * rp;
+    T rp = T(1);
+    { const T m = __ldg(Ms + 0) * rp;
       L[0] = D[0] * m;
       L[1] = D[1] * m;
       L[2] = D[2] * m;
@@ -133,48 +142,48 @@ __device__ __forceinline__ void m2l_side_a_2(const float (&D)[10], const float *
       L[9] = D[9] * m;
     }
     rp *= rho;
-    { const float m = -__ldg(Ms + 1) * rp;
-      L[0] = fmaf(D[1], m, L[0]);
-      L[1] = fmaf(D[4], m, L[1]);
-      L[2] = fmaf(D[5], m, L[2]);
-      L[3] = fmaf(D[6], m, L[3]);
+    { const T m = -__ldg(Ms + 1) * rp;
+      L[0] = m2l_fma(D[1], m, L[0]);
+      L[1] = m2l_fma(D[4], m, L[1]);
+      L[2] = m2l_fma(D[5], m, L[2]);
+      L[3] = m2l_fma(D[6], m, L[3]);
     }
-    { const float m = -__ldg(Ms + 2) * rp;
-      L[0] = fmaf(D[2], m, L[0]);
-      L[1] = fmaf(D[5], m, L[1]);
-      L[2] = fmaf(D[7], m, L[2]);
-      L[3] = fmaf(D[8], m, L[3]);
+    { const T m = -__ldg(Ms + 2) * rp;
+      L[0] = m2l_fma(D[2], m, L[0]);
+      L[1] = m2l_fma(D[5], m, L[1]);
+      L[2] = m2l_fma(D[7], m, L[2]);
+      L[3] = m2l_fma(D[8], m, L[3]);
     }
-    { const float m = -__ldg(Ms + 3) * rp;
-      L[0] = fmaf(D[3], m, L[0]);
-      L[1] = fmaf(D[6], m, L[1]);
-      L[2] = fmaf(D[8], m, L[2]);
-      L[3] = fmaf(D[9], m, L[3]);
+    { const T m = -__ldg(Ms + 3) * rp;
+      L[0] = m2l_fma(D[3], m, L[0]);
+      L[1] = m2l_fma(D[6], m, L[1]);
+      L[2] = m2l_fma(D[8], m, L[2]);
+      L[3] = m2l_fma(D[9], m, L[3]);
     }
     rp *= rho;
-    { const float m = __ldg(Ms + 4) * rp;
-      L[0] = fmaf(D[4], m, L[0]);
+    { const T m = __ldg(Ms + 4) * rp;
+      L[0] = m2l_fma(D[4], m, L[0]);
     }
-    { const float m = __ldg(Ms + 5) * rp;
-      L[0] = fmaf(D[5], m, L[0]);
+    { const T m = __ldg(Ms + 5) * rp;
+      L[0] = m2l_fma(D[5], m, L[0]);
     }
-    { const float m = __ldg(Ms + 6) * rp;
-      L[0] = fmaf(D[6], m, L[0]);
+    { const T m = __ldg(Ms + 6) * rp;
+      L[0] = m2l_fma(D[6], m, L[0]);
     }
-    { const float m = __ldg(Ms + 7) * rp;
-      L[0] = fmaf(D[7], m, L[0]);
+    { const T m = __ldg(Ms + 7) * rp;
+      L[0] = m2l_fma(D[7], m, L[0]);
     }
-    { const float m = __ldg(Ms + 8) * rp;
-      L[0] = fmaf(D[8], m, L[0]);
+    { const T m = __ldg(Ms + 8) * rp;
+      L[0] = m2l_fma(D[8], m, L[0]);
     }
-    { const float m = __ldg(Ms + 9) * rp;
-      L[0] = fmaf(D[9], m, L[0]);
+    { const T m = __ldg(Ms + 9) * rp;
+      L[0] = m2l_fma(D[9], m, L[0]);
     }
 }
 
-__device__ __forceinline__ void m2l_side_b_2(const float (&D)[10], const float *__restrict__ Ms, float (&L)[10])
+template <class T> __device__ __forceinline__ void m2l_side_b_2(const T (&D)[10], const T *__restrict__ Ms, T (&L)[10])
 {
-    { const float m = __ldg(Ms + 0);
+    { const T m = __ldg(Ms + 0);
       L[0] = D[0] * m;
       L[1] = -D[1] * m;
       L[2] = -D[2] * m;
@@ -186,49 +195,49 @@ __device__ __forceinline__ void m2l_side_b_2(const float (&D)[10], const float *
       L[8] = D[8] * m;
       L[9] = D[9] * m;
     }
-    { const float m = __ldg(Ms + 1);
-      L[0] = fmaf(D[1], m, L[0]);
-      L[1] = fmaf(-D[4], m, L[1]);
-      L[2] = fmaf(-D[5], m, L[2]);
-      L[3] = fmaf(-D[6], m, L[3]);
+    { const T m = __ldg(Ms + 1);
+      L[0] = m2l_fma(D[1], m, L[0]);
+      L[1] = m2l_fma(-D[4], m, L[1]);
+      L[2] = m2l_fma(-D[5], m, L[2]);
+      L[3] = m2l_fma(-D[6], m, L[3]);
     }
-    { const float m = __ldg(Ms + 2);
-      L[0] = fmaf(D[2], m, L[0]);
-      L[1] = fmaf(-D[5], m, L[1]);
-      L[2] = fmaf(-D[7], m, L[2]);
-      L[3] = fmaf(-D[8], m, L[3]);
+    { const T m = __ldg(Ms + 2);
+      L[0] = m2l_fma(D[2], m, L[0]);
+      L[1] = m2l_fma(-D[5], m, L[1]);
+      L[2] = m2l_fma(-D[7], m, L[2]);
+      L[3] = m2l_fma(-D[8], m, L[3]);
     }
-    { const float m = __ldg(Ms + 3);
-      L[0] = fmaf(D[3], m, L[0]);
-      L[1] = fmaf(-D[6], m, L[1]);
-      L[2] = fmaf(-D[8], m, L[2]);
-      L[3] = fmaf(-D[9], m, L[3]);
+    { const T m = __ldg(Ms + 3);
+      L[0] = m2l_fma(D[3], m, L[0]);
+      L[1] = m2l_fma(-D[6], m, L[1]);
+      L[2] = m2l_fma(-D[8], m, L[2]);
+      L[3] = m2l_fma(-D[9], m, L[3]);
     }
-    { const float m = __ldg(Ms + 4);
-      L[0] = fmaf(D[4], m, L[0]);
+    { const T m = __ldg(Ms + 4);
+      L[0] = m2l_fma(D[4], m, L[0]);
     }
-    { const float m = __ldg(Ms + 5);
-      L[0] = fmaf(D[5], m, L[0]);
+    { const T m = __ldg(Ms + 5);
+      L[0] = m2l_fma(D[5], m, L[0]);
     }
-    { const float m = __ldg(Ms + 6);
-      L[0] = fmaf(D[6], m, L[0]);
+    { const T m = __ldg(Ms + 6);
+      L[0] = m2l_fma(D[6], m, L[0]);
     }
-    { const float m = __ldg(Ms + 7);
-      L[0] = fmaf(D[7], m, L[0]);
+    { const T m = __ldg(Ms + 7);
+      L[0] = m2l_fma(D[7], m, L[0]);
     }
-    { const float m = __ldg(Ms + 8);
-      L[0] = fmaf(D[8], m, L[0]);
+    { const T m = __ldg(Ms + 8);
+      L[0] = m2l_fma(D[8], m, L[0]);
     }
-    { const float m = __ldg(Ms + 9);
-      L[0] = fmaf(D[9], m, L[0]);
+    { const T m = __ldg(Ms + 9);
+      L[0] = m2l_fma(D[9], m, L[0]);
     }
 }
 
-__device__ __forceinline__ void m2l_side_a_forces_2(const float (&D)[10], const float *__restrict__ Ms, float rho, float (&L)[10])
+template <class T> __device__ __forceinline__ void m2l_side_a_forces_2(const T (&D)[10], const T *__restrict__ Ms, T rho, T (&L)[10])
 {
-    L[0] = 0.0f;
-    float rp = 1.0f;
-    { const float m = __ldg(Ms + 0) * rp;
+    L[0] = T(0);
+    T rp = T(1);
+    { const T m = __ldg(Ms + 0) * rp;
       L[1] = D[1] * m;
       L[2] = D[2] * m;
       L[3] = D[3] * m;
@@ -240,27 +249,27 @@ __device__ __forceinline__ void m2l_side_a_forces_2(const float (&D)[10], const 
       L[9] = D[9] * m;
     }
     rp *= rho;
-    { const float m = -__ldg(Ms + 1) * rp;
-      L[1] = fmaf(D[4], m, L[1]);
-      L[2] = fmaf(D[5], m, L[2]);
-      L[3] = fmaf(D[6], m, L[3]);
+    { const T m = -__ldg(Ms + 1) * rp;
+      L[1] = m2l_fma(D[4], m, L[1]);
+      L[2] = m2l_fma(D[5], m, L[2]);
+      L[3] = m2l_fma(D[6], m, L[3]);
     }
-    { const float m = -__ldg(Ms + 2) * rp;
-      L[1] = fmaf(D[5], m, L[1]);
-      L[2] = fmaf(D[7], m, L[2]);
-      L[3] = fmaf(D[8], m, L[3]);
+    { const T m = -__ldg(Ms + 2) * rp;
+      L[1] = m2l_fma(D[5], m, L[1]);
+      L[2] = m2l_fma(D[7], m, L[2]);
+      L[3] = m2l_fma(D[8], m, L[3]);
     }
-    { const float m = -__ldg(Ms + 3) * rp;
-      L[1] = fmaf(D[6], m, L[1]);
-      L[2] = fmaf(D[8], m, L[2]);
-      L[3] = fmaf(D[9], m, L[3]);
+    { const T m = -__ldg(Ms + 3) * rp;
+      L[1] = m2l_fma(D[6], m, L[1]);
+      L[2] = m2l_fma(D[8], m, L[2]);
+      L[3] = m2l_fma(D[9], m, L[3]);
     }
 }
 
-__device__ __forceinline__ void m2l_side_b_forces_2(const float (&D)[10], const float *__restrict__ Ms, float (&L)[10])
+template <class T> __device__ __forceinline__ void m2l_side_b_forces_2(const T (&D)[10], const T *__restrict__ Ms, T (&L)[10])
 {
-    L[0] = 0.0f;
-    { const float m = __ldg(Ms + 0);
+    L[0] = T(0);
+    { const T m = __ldg(Ms + 0);
       L[1] = -D[1] * m;
       L[2] = -D[2] * m;
       L[3] = -D[3] * m;
@@ -271,68 +280,67 @@ __device__ __forceinline__ void m2l_side_b_forces_2(const float (&D)[10], const 
       L[8] = D[8] * m;
       L[9] = D[9] * m;
     }
-    { const float m = __ldg(Ms + 1);
-      L[1] = fmaf(-D[4], m, L[1]);
-      L[2] = fmaf(-D[5], m, L[2]);
-      L[3] = fmaf(-D[6], m, L[3]);
+    { const T m = __ldg(Ms + 1);
+      L[1] = m2l_fma(-D[4], m, L[1]);
+      L[2] = m2l_fma(-D[5], m, L[2]);
+      L[3] = m2l_fma(-D[6], m, L[3]);
     }
-    { const float m = __ldg(Ms + 2);
-      L[1] = fmaf(-D[5], m, L[1]);
-      L[2] = fmaf(-D[7], m, L[2]);
-      L[3] = fmaf(-D[8], m, L[3]);
+    { const T m = __ldg(Ms + 2);
+      L[1] = m2l_fma(-D[5], m, L[1]);
+      L[2] = m2l_fma(-D[7], m, L[2]);
+      L[3] = m2l_fma(-D[8], m, L[3]);
     }
-    { const float m = __ldg(Ms + 3);
-      L[1] = fmaf(-D[6], m, L[1]);
-      L[2] = fmaf(-D[8], m, L[2]);
-      L[3] = fmaf(-D[9], m, L[3]);
+    { const T m = __ldg(Ms + 3);
+      L[1] = m2l_fma(-D[6], m, L[1]);
+      L[2] = m2l_fma(-D[8], m, L[2]);
+      L[3] = m2l_fma(-D[9], m, L[3]);
     }
 }
 
-__device__ __forceinline__ void m2l_dtensor_3(float dx, float dy, float dz, float soft2, float (&D)[20])
+template <class T> __device__ __forceinline__ void m2l_dtensor_3(T dx, T dy, T dz, T soft2, T (&D)[20])
 {
-    const float s2 = fmaf(dx, dx, fmaf(dy, dy, fmaf(dz, dz, soft2)));
-    float si = rsqrtf(s2);
-    si = si * fmaf(-0.5f * s2, si * si, 1.5f);   // one Newton step
-    const float si2 = si * si;
-    const float f0 = -si;
-    const float f1 = -1.0f * f0 * si2;
-    const float f2 = -3.0f * f1 * si2;
-    const float f3 = -5.0f * f2 * si2;
-    const float r_0_0 = f0;
-    const float r_1_0 = f1;
-    const float r_2_0 = f2;
-    const float r_3_0 = f3;
-    const float r_0_1 = dx * r_1_0;
-    const float r_1_1 = dx * r_2_0;
-    const float r_2_1 = dx * r_3_0;
-    const float r_0_2 = dy * r_1_0;
-    const float r_1_2 = dy * r_2_0;
-    const float r_2_2 = dy * r_3_0;
-    const float r_0_3 = dz * r_1_0;
-    const float r_1_3 = dz * r_2_0;
-    const float r_2_3 = dz * r_3_0;
-    const float r_0_4 = fmaf(1.0f, r_1_0, dx * r_1_1);
-    const float r_1_4 = fmaf(1.0f, r_2_0, dx * r_2_1);
-    const float r_0_5 = dx * r_1_2;
-    const float r_1_5 = dx * r_2_2;
-    const float r_0_6 = dx * r_1_3;
-    const float r_1_6 = dx * r_2_3;
-    const float r_0_7 = fmaf(1.0f, r_1_0, dy * r_1_2);
-    const float r_1_7 = fmaf(1.0f, r_2_0, dy * r_2_2);
-    const float r_0_8 = dy * r_1_3;
-    const float r_1_8 = dy * r_2_3;
-    const float r_0_9 = fmaf(1.0f, r_1_0, dz * r_1_3);
-    const float r_1_9 = fmaf(1.0f, r_2_0, dz * r_2_3);
-    const float r_0_10 = fmaf(2.0f, r_1_1, dx * r_1_4);
-    const float r_0_11 = fmaf(1.0f, r_1_2, dx * r_1_5);
-    const float r_0_12 = fmaf(1.0f, r_1_3, dx * r_1_6);
-    const float r_0_13 = dx * r_1_7;
-    const float r_0_14 = dx * r_1_8;
-    const float r_0_15 = dx * r_1_9;
-    const float r_0_16 = fmaf(2.0f, r_1_2, dy * r_1_7);
-    const float r_0_17 = fmaf(1.0f, r_1_3, dy * r_1_8);
-    const float r_0_18 = dy * r_1_9;
-    const float r_0_19 = fmaf(2.0f, r_1_3, dz * r_1_9);
+    const T s2 = m2l_fma(dx, dx, m2l_fma(dy, dy, m2l_fma(dz, dz, soft2)));
+    const T si = m2l_rsqrt(s2);
+    const T si2 = si * si;
+    const T f0 = -si;
+    const T f1 = T(-1) * f0 * si2;
+    const T f2 = T(-3) * f1 * si2;
+    const T f3 = T(-5) * f2 * si2;
+    const T r_0_0 = f0;
+    const T r_1_0 = f1;
+    const T r_2_0 = f2;
+    const T r_3_0 = f3;
+    const T r_0_1 = dx * r_1_0;
+    const T r_1_1 = dx * r_2_0;
+    const T r_2_1 = dx * r_3_0;
+    const T r_0_2 = dy * r_1_0;
+    const T r_1_2 = dy * r_2_0;
+    const T r_2_2 = dy * r_3_0;
+    const T r_0_3 = dz * r_1_0;
+    const T r_1_3 = dz * r_2_0;
+    const T r_2_3 = dz * r_3_0;
+    const T r_0_4 = m2l_fma(T(1), r_1_0, dx * r_1_1);
+    const T r_1_4 = m2l_fma(T(1), r_2_0, dx * r_2_1);
+    const T r_0_5 = dx * r_1_2;
+    const T r_1_5 = dx * r_2_2;
+    const T r_0_6 = dx * r_1_3;
+    const T r_1_6 = dx * r_2_3;
+    const T r_0_7 = m2l_fma(T(1), r_1_0, dy * r_1_2);
+    const T r_1_7 = m2l_fma(T(1), r_2_0, dy * r_2_2);
+    const T r_0_8 = dy * r_1_3;
+    const T r_1_8 = dy * r_2_3;
+    const T r_0_9 = m2l_fma(T(1), r_1_0, dz * r_1_3);
+    const T r_1_9 = m2l_fma(T(1), r_2_0, dz * r_2_3);
+    const T r_0_10 = m2l_fma(T(2), r_1_1, dx * r_1_4);
+    const T r_0_11 = m2l_fma(T(1), r_1_2, dx * r_1_5);
+    const T r_0_12 = m2l_fma(T(1), r_1_3, dx * r_1_6);
+    const T r_0_13 = dx * r_1_7;
+    const T r_0_14 = dx * r_1_8;
+    const T r_0_15 = dx * r_1_9;
+    const T r_0_16 = m2l_fma(T(2), r_1_2, dy * r_1_7);
+    const T r_0_17 = m2l_fma(T(1), r_1_3, dy * r_1_8);
+    const T r_0_18 = dy * r_1_9;
+    const T r_0_19 = m2l_fma(T(2), r_1_3, dz * r_1_9);
     D[0] = r_0_0;
     D[1] = r_0_1;
     D[2] = r_0_2;
@@ -355,10 +363,10 @@ __device__ __forceinline__ void m2l_dtensor_3(float dx, float dy, float dz, floa
     D[19] = r_0_19;
 }
 
-__device__ __forceinline__ void m2l_side_a_3(const float (&D)[20], const float *__restrict__ Ms, float rho, float (&L)[20])
+template <class T> __device__ __forceinline__ void m2l_side_a_3(const T (&D)[20], const T *__restrict__ Ms, T rho, T (&L)[20])
 {
-    float rp = 1.0f;
-    { const float m = __ldg(Ms + 0) * rp;
+    T rp = T(1);
+    { const T m = __ldg(Ms + 0) * rp;
       L[0] = D[0] * m;
       L[1] = D[1] * m;
       L[2] = D[2] * m;
@@ -381,115 +389,115 @@ __device__ __forceinline__ void m2l_side_a_3(const float (&D)[20], const float *
       L[19] = D[19] * m;
     }
     rp *= rho;
-    { const float m = -__ldg(Ms + 1) * rp;
-      L[0] = fmaf(D[1], m, L[0]);
-      L[1] = fmaf(D[4], m, L[1]);
-      L[2] = fmaf(D[5], m, L[2]);
-      L[3] = fmaf(D[6], m, L[3]);
-      L[4] = fmaf(D[10], m, L[4]);
-      L[5] = fmaf(D[11], m, L[5]);
-      L[6] = fmaf(D[12], m, L[6]);
-      L[7] = fmaf(D[13], m, L[7]);
-      L[8] = fmaf(D[14], m, L[8]);
-      L[9] = fmaf(D[15], m, L[9]);
+    { const T m = -__ldg(Ms + 1) * rp;
+      L[0] = m2l_fma(D[1], m, L[0]);
+      L[1] = m2l_fma(D[4], m, L[1]);
+      L[2] = m2l_fma(D[5], m, L[2]);
+      L[3] = m2l_fma(D[6], m, L[3]);
+      L[4] = m2l_fma(D[10], m, L[4]);
+      L[5] = m2l_fma(D[11], m, L[5]);
+      L[6] = m2l_fma(D[12], m, L[6]);
+      L[7] = m2l_fma(D[13], m, L[7]);
+      L[8] = m2l_fma(D[14], m, L[8]);
+      L[9] = m2l_fma(D[15], m, L[9]);
     }
-    { const float m = -__ldg(Ms + 2) * rp;
-      L[0] = fmaf(D[2], m, L[0]);
-      L[1] = fmaf(D[5], m, L[1]);
-      L[2] = fmaf(D[7], m, L[2]);
-      L[3] = fmaf(D[8], m, L[3]);
-      L[4] = fmaf(D[11], m, L[4]);
-      L[5] = fmaf(D[13], m, L[5]);
-      L[6] = fmaf(D[14], m, L[6]);
-      L[7] = fmaf(D[16], m, L[7]);
-      L[8] = fmaf(D[17], m, L[8]);
-      L[9] = fmaf(D[18], m, L[9]);
+    { const T m = -__ldg(Ms + 2) * rp;
+      L[0] = m2l_fma(D[2], m, L[0]);
+      L[1] = m2l_fma(D[5], m, L[1]);
+      L[2] = m2l_fma(D[7], m, L[2]);
+      L[3] = m2l_fma(D[8], m, L[3]);
+      L[4] = m2l_fma(D[11], m, L[4]);
+      L[5] = m2l_fma(D[13], m, L[5]);
+      L[6] = m2l_fma(D[14], m, L[6]);
+      L[7] = m2l_fma(D[16], m, L[7]);
+      L[8] = m2l_fma(D[17], m, L[8]);
+      L[9] = m2l_fma(D[18], m, L[9]);
     }
-    { const float m = -__ldg(Ms + 3) * rp;
-      L[0] = fmaf(D[3], m, L[0]);
-      L[1] = fmaf(D[6], m, L[1]);
-      L[2] = fmaf(D[8], m, L[2]);
-      L[3] = fmaf(D[9], m, L[3]);
-      L[4] = fmaf(D[12], m, L[4]);
-      L[5] = fmaf(D[14], m, L[5]);
-      L[6] = fmaf(D[15], m, L[6]);
-      L[7] = fmaf(D[17], m, L[7]);
-      L[8] = fmaf(D[18], m, L[8]);
-      L[9] = fmaf(D[19], m, L[9]);
-    }
-    rp *= rho;
-    { const float m = __ldg(Ms + 4) * rp;
-      L[0] = fmaf(D[4], m, L[0]);
-      L[1] = fmaf(D[10], m, L[1]);
-      L[2] = fmaf(D[11], m, L[2]);
-      L[3] = fmaf(D[12], m, L[3]);
-    }
-    { const float m = __ldg(Ms + 5) * rp;
-      L[0] = fmaf(D[5], m, L[0]);
-      L[1] = fmaf(D[11], m, L[1]);
-      L[2] = fmaf(D[13], m, L[2]);
-      L[3] = fmaf(D[14], m, L[3]);
-    }
-    { const float m = __ldg(Ms + 6) * rp;
-      L[0] = fmaf(D[6], m, L[0]);
-      L[1] = fmaf(D[12], m, L[1]);
-      L[2] = fmaf(D[14], m, L[2]);
-      L[3] = fmaf(D[15], m, L[3]);
-    }
-    { const float m = __ldg(Ms + 7) * rp;
-      L[0] = fmaf(D[7], m, L[0]);
-      L[1] = fmaf(D[13], m, L[1]);
-      L[2] = fmaf(D[16], m, L[2]);
-      L[3] = fmaf(D[17], m, L[3]);
-    }
-    { const float m = __ldg(Ms + 8) * rp;
-      L[0] = fmaf(D[8], m, L[0]);
-      L[1] = fmaf(D[14], m, L[1]);
-      L[2] = fmaf(D[17], m, L[2]);
-      L[3] = fmaf(D[18], m, L[3]);
-    }
-    { const float m = __ldg(Ms + 9) * rp;
-      L[0] = fmaf(D[9], m, L[0]);
-      L[1] = fmaf(D[15], m, L[1]);
-      L[2] = fmaf(D[18], m, L[2]);
-      L[3] = fmaf(D[19], m, L[3]);
+    { const T m = -__ldg(Ms + 3) * rp;
+      L[0] = m2l_fma(D[3], m, L[0]);
+      L[1] = m2l_fma(D[6], m, L[1]);
+      L[2] = m2l_fma(D[8], m, L[2]);
+      L[3] = m2l_fma(D[9], m, L[3]);
+      L[4] = m2l_fma(D[12], m, L[4]);
+      L[5] = m2l_fma(D[14], m, L[5]);
+      L[6] = m2l_fma(D[15], m, L[6]);
+      L[7] = m2l_fma(D[17], m, L[7]);
+      L[8] = m2l_fma(D[18], m, L[8]);
+      L[9] = m2l_fma(D[19], m, L[9]);
     }
     rp *= rho;
-    { const float m = -__ldg(Ms + 10) * rp;
-      L[0] = fmaf(D[10], m, L[0]);
+    { const T m = __ldg(Ms + 4) * rp;
+      L[0] = m2l_fma(D[4], m, L[0]);
+      L[1] = m2l_fma(D[10], m, L[1]);
+      L[2] = m2l_fma(D[11], m, L[2]);
+      L[3] = m2l_fma(D[12], m, L[3]);
     }
-    { const float m = -__ldg(Ms + 11) * rp;
-      L[0] = fmaf(D[11], m, L[0]);
+    { const T m = __ldg(Ms + 5) * rp;
+      L[0] = m2l_fma(D[5], m, L[0]);
+      L[1] = m2l_fma(D[11], m, L[1]);
+      L[2] = m2l_fma(D[13], m, L[2]);
+      L[3] = m2l_fma(D[14], m, L[3]);
     }
-    { const float m = -__ldg(Ms + 12) * rp;
-      L[0] = fmaf(D[12], m, L[0]);
+    { const T m = __ldg(Ms + 6) * rp;
+      L[0] = m2l_fma(D[6], m, L[0]);
+      L[1] = m2l_fma(D[12], m, L[1]);
+      L[2] = m2l_fma(D[14], m, L[2]);
+      L[3] = m2l_fma(D[15], m, L[3]);
     }
-    { const float m = -__ldg(Ms + 13) * rp;
-      L[0] = fmaf(D[13], m, L[0]);
+    { const T m = __ldg(Ms + 7) * rp;
+      L[0] = m2l_fma(D[7], m, L[0]);
+      L[1] = m2l_fma(D[13], m, L[1]);
+      L[2] = m2l_fma(D[16], m, L[2]);
+      L[3] = m2l_fma(D[17], m, L[3]);
     }
-    { const float m = -__ldg(Ms + 14) * rp;
-      L[0] = fmaf(D[14], m, L[0]);
+    { const T m = __ldg(Ms + 8) * rp;
+      L[0] = m2l_fma(D[8], m, L[0]);
+      L[1] = m2l_fma(D[14], m, L[1]);
+      L[2] = m2l_fma(D[17], m, L[2]);
+      L[3] = m2l_fma(D[18], m, L[3]);
     }
-    { const float m = -__ldg(Ms + 15) * rp;
-      L[0] = fmaf(D[15], m, L[0]);
+    { const T m = __ldg(Ms + 9) * rp;
+      L[0] = m2l_fma(D[9], m, L[0]);
+      L[1] = m2l_fma(D[15], m, L[1]);
+      L[2] = m2l_fma(D[18], m, L[2]);
+      L[3] = m2l_fma(D[19], m, L[3]);
     }
-    { const float m = -__ldg(Ms + 16) * rp;
-      L[0] = fmaf(D[16], m, L[0]);
+    rp *= rho;
+    { const T m = -__ldg(Ms + 10) * rp;
+      L[0] = m2l_fma(D[10], m, L[0]);
     }
-    { const float m = -__ldg(Ms + 17) * rp;
-      L[0] = fmaf(D[17], m, L[0]);
+    { const T m = -__ldg(Ms + 11) * rp;
+      L[0] = m2l_fma(D[11], m, L[0]);
     }
-    { const float m = -__ldg(Ms + 18) * rp;
-      L[0] = fmaf(D[18], m, L[0]);
+    { const T m = -__ldg(Ms + 12) * rp;
+      L[0] = m2l_fma(D[12], m, L[0]);
     }
-    { const float m = -__ldg(Ms + 19) * rp;
-      L[0] = fmaf(D[19], m, L[0]);
+    { const T m = -__ldg(Ms + 13) * rp;
+      L[0] = m2l_fma(D[13], m, L[0]);
+    }
+    { const T m = -__ldg(Ms + 14) * rp;
+      L[0] = m2l_fma(D[14], m, L[0]);
+    }
+    { const T m = -__ldg(Ms + 15) * rp;
+      L[0] = m2l_fma(D[15], m, L[0]);
+    }
+    { const T m = -__ldg(Ms + 16) * rp;
+      L[0] = m2l_fma(D[16], m, L[0]);
+    }
+    { const T m = -__ldg(Ms + 17) * rp;
+      L[0] = m2l_fma(D[17], m, L[0]);
+    }
+    { const T m = -__ldg(Ms + 18) * rp;
+      L[0] = m2l_fma(D[18], m, L[0]);
+    }
+    { const T m = -__ldg(Ms + 19) * rp;
+      L[0] = m2l_fma(D[19], m, L[0]);
     }
 }
 
-__device__ __forceinline__ void m2l_side_b_3(const float (&D)[20], const float *__restrict__ Ms, float (&L)[20])
+template <class T> __device__ __forceinline__ void m2l_side_b_3(const T (&D)[20], const T *__restrict__ Ms, T (&L)[20])
 {
-    { const float m = __ldg(Ms + 0);
+    { const T m = __ldg(Ms + 0);
       L[0] = D[0] * m;
       L[1] = -D[1] * m;
       L[2] = -D[2] * m;
@@ -511,115 +519,115 @@ __device__ __forceinline__ void m2l_side_b_3(const float (&D)[20], const float *
       L[18] = -D[18] * m;
       L[19] = -D[19] * m;
     }
-    { const float m = __ldg(Ms + 1);
-      L[0] = fmaf(D[1], m, L[0]);
-      L[1] = fmaf(-D[4], m, L[1]);
-      L[2] = fmaf(-D[5], m, L[2]);
-      L[3] = fmaf(-D[6], m, L[3]);
-      L[4] = fmaf(D[10], m, L[4]);
-      L[5] = fmaf(D[11], m, L[5]);
-      L[6] = fmaf(D[12], m, L[6]);
-      L[7] = fmaf(D[13], m, L[7]);
-      L[8] = fmaf(D[14], m, L[8]);
-      L[9] = fmaf(D[15], m, L[9]);
+    { const T m = __ldg(Ms + 1);
+      L[0] = m2l_fma(D[1], m, L[0]);
+      L[1] = m2l_fma(-D[4], m, L[1]);
+      L[2] = m2l_fma(-D[5], m, L[2]);
+      L[3] = m2l_fma(-D[6], m, L[3]);
+      L[4] = m2l_fma(D[10], m, L[4]);
+      L[5] = m2l_fma(D[11], m, L[5]);
+      L[6] = m2l_fma(D[12], m, L[6]);
+      L[7] = m2l_fma(D[13], m, L[7]);
+      L[8] = m2l_fma(D[14], m, L[8]);
+      L[9] = m2l_fma(D[15], m, L[9]);
     }
-    { const float m = __ldg(Ms + 2);
-      L[0] = fmaf(D[2], m, L[0]);
-      L[1] = fmaf(-D[5], m, L[1]);
-      L[2] = fmaf(-D[7], m, L[2]);
-      L[3] = fmaf(-D[8], m, L[3]);
-      L[4] = fmaf(D[11], m, L[4]);
-      L[5] = fmaf(D[13], m, L[5]);
-      L[6] = fmaf(D[14], m, L[6]);
-      L[7] = fmaf(D[16], m, L[7]);
-      L[8] = fmaf(D[17], m, L[8]);
-      L[9] = fmaf(D[18], m, L[9]);
+    { const T m = __ldg(Ms + 2);
+      L[0] = m2l_fma(D[2], m, L[0]);
+      L[1] = m2l_fma(-D[5], m, L[1]);
+      L[2] = m2l_fma(-D[7], m, L[2]);
+      L[3] = m2l_fma(-D[8], m, L[3]);
+      L[4] = m2l_fma(D[11], m, L[4]);
+      L[5] = m2l_fma(D[13], m, L[5]);
+      L[6] = m2l_fma(D[14], m, L[6]);
+      L[7] = m2l_fma(D[16], m, L[7]);
+      L[8] = m2l_fma(D[17], m, L[8]);
+      L[9] = m2l_fma(D[18], m, L[9]);
     }
-    { const float m = __ldg(Ms + 3);
-      L[0] = fmaf(D[3], m, L[0]);
-      L[1] = fmaf(-D[6], m, L[1]);
-      L[2] = fmaf(-D[8], m, L[2]);
-      L[3] = fmaf(-D[9], m, L[3]);
-      L[4] = fmaf(D[12], m, L[4]);
-      L[5] = fmaf(D[14], m, L[5]);
-      L[6] = fmaf(D[15], m, L[6]);
-      L[7] = fmaf(D[17], m, L[7]);
-      L[8] = fmaf(D[18], m, L[8]);
-      L[9] = fmaf(D[19], m, L[9]);
+    { const T m = __ldg(Ms + 3);
+      L[0] = m2l_fma(D[3], m, L[0]);
+      L[1] = m2l_fma(-D[6], m, L[1]);
+      L[2] = m2l_fma(-D[8], m, L[2]);
+      L[3] = m2l_fma(-D[9], m, L[3]);
+      L[4] = m2l_fma(D[12], m, L[4]);
+      L[5] = m2l_fma(D[14], m, L[5]);
+      L[6] = m2l_fma(D[15], m, L[6]);
+      L[7] = m2l_fma(D[17], m, L[7]);
+      L[8] = m2l_fma(D[18], m, L[8]);
+      L[9] = m2l_fma(D[19], m, L[9]);
     }
-    { const float m = __ldg(Ms + 4);
-      L[0] = fmaf(D[4], m, L[0]);
-      L[1] = fmaf(-D[10], m, L[1]);
-      L[2] = fmaf(-D[11], m, L[2]);
-      L[3] = fmaf(-D[12], m, L[3]);
+    { const T m = __ldg(Ms + 4);
+      L[0] = m2l_fma(D[4], m, L[0]);
+      L[1] = m2l_fma(-D[10], m, L[1]);
+      L[2] = m2l_fma(-D[11], m, L[2]);
+      L[3] = m2l_fma(-D[12], m, L[3]);
     }
-    { const float m = __ldg(Ms + 5);
-      L[0] = fmaf(D[5], m, L[0]);
-      L[1] = fmaf(-D[11], m, L[1]);
-      L[2] = fmaf(-D[13], m, L[2]);
-      L[3] = fmaf(-D[14], m, L[3]);
+    { const T m = __ldg(Ms + 5);
+      L[0] = m2l_fma(D[5], m, L[0]);
+      L[1] = m2l_fma(-D[11], m, L[1]);
+      L[2] = m2l_fma(-D[13], m, L[2]);
+      L[3] = m2l_fma(-D[14], m, L[3]);
     }
-    { const float m = __ldg(Ms + 6);
-      L[0] = fmaf(D[6], m, L[0]);
-      L[1] = fmaf(-D[12], m, L[1]);
-      L[2] = fmaf(-D[14], m, L[2]);
-      L[3] = fmaf(-D[15], m, L[3]);
+    { const T m = __ldg(Ms + 6);
+      L[0] = m2l_fma(D[6], m, L[0]);
+      L[1] = m2l_fma(-D[12], m, L[1]);
+      L[2] = m2l_fma(-D[14], m, L[2]);
+      L[3] = m2l_fma(-D[15], m, L[3]);
     }
-    { const float m = __ldg(Ms + 7);
-      L[0] = fmaf(D[7], m, L[0]);
-      L[1] = fmaf(-D[13], m, L[1]);
-      L[2] = fmaf(-D[16], m, L[2]);
-      L[3] = fmaf(-D[17], m, L[3]);
+    { const T m = __ldg(Ms + 7);
+      L[0] = m2l_fma(D[7], m, L[0]);
+      L[1] = m2l_fma(-D[13], m, L[1]);
+      L[2] = m2l_fma(-D[16], m, L[2]);
+      L[3] = m2l_fma(-D[17], m, L[3]);
     }
-    { const float m = __ldg(Ms + 8);
-      L[0] = fmaf(D[8], m, L[0]);
-      L[1] = fmaf(-D[14], m, L[1]);
-      L[2] = fmaf(-D[17], m, L[2]);
-      L[3] = fmaf(-D[18], m, L[3]);
+    { const T m = __ldg(Ms + 8);
+      L[0] = m2l_fma(D[8], m, L[0]);
+      L[1] = m2l_fma(-D[14], m, L[1]);
+      L[2] = m2l_fma(-D[17], m, L[2]);
+      L[3] = m2l_fma(-D[18], m, L[3]);
     }
-    { const float m = __ldg(Ms + 9);
-      L[0] = fmaf(D[9], m, L[0]);
-      L[1] = fmaf(-D[15], m, L[1]);
-      L[2] = fmaf(-D[18], m, L[2]);
-      L[3] = fmaf(-D[19], m, L[3]);
+    { const T m = __ldg(Ms + 9);
+      L[0] = m2l_fma(D[9], m, L[0]);
+      L[1] = m2l_fma(-D[15], m, L[1]);
+      L[2] = m2l_fma(-D[18], m, L[2]);
+      L[3] = m2l_fma(-D[19], m, L[3]);
     }
-    { const float m = __ldg(Ms + 10);
-      L[0] = fmaf(D[10], m, L[0]);
+    { const T m = __ldg(Ms + 10);
+      L[0] = m2l_fma(D[10], m, L[0]);
     }
-    { const float m = __ldg(Ms + 11);
-      L[0] = fmaf(D[11], m, L[0]);
+    { const T m = __ldg(Ms + 11);
+      L[0] = m2l_fma(D[11], m, L[0]);
     }
-    { const float m = __ldg(Ms + 12);
-      L[0] = fmaf(D[12], m, L[0]);
+    { const T m = __ldg(Ms + 12);
+      L[0] = m2l_fma(D[12], m, L[0]);
     }
-    { const float m = __ldg(Ms + 13);
-      L[0] = fmaf(D[13], m, L[0]);
+    { const T m = __ldg(Ms + 13);
+      L[0] = m2l_fma(D[13], m, L[0]);
     }
-    { const float m = __ldg(Ms + 14);
-      L[0] = fmaf(D[14], m, L[0]);
+    { const T m = __ldg(Ms + 14);
+      L[0] = m2l_fma(D[14], m, L[0]);
     }
-    { const float m = __ldg(Ms + 15);
-      L[0] = fmaf(D[15], m, L[0]);
+    { const T m = __ldg(Ms + 15);
+      L[0] = m2l_fma(D[15], m, L[0]);
     }
-    { const float m = __ldg(Ms + 16);
-      L[0] = fmaf(D[16], m, L[0]);
+    { const T m = __ldg(Ms + 16);
+      L[0] = m2l_fma(D[16], m, L[0]);
     }
-    { const float m = __ldg(Ms + 17);
-      L[0] = fmaf(D[17], m, L[0]);
+    { const T m = __ldg(Ms + 17);
+      L[0] = m2l_fma(D[17], m, L[0]);
     }
-    { const float m = __ldg(Ms + 18);
-      L[0] = fmaf(D[18], m, L[0]);
+    { const T m = __ldg(Ms + 18);
+      L[0] = m2l_fma(D[18], m, L[0]);
     }
-    { const float m = __ldg(Ms + 19);
-      L[0] = fmaf(D[19], m, L[0]);
+    { const T m = __ldg(Ms + 19);
+      L[0] = m2l_fma(D[19], m, L[0]);
     }
 }
 
-__device__ __forceinline__ void m2l_side_a_forces_3(const float (&D)[20], const float *__restrict__ Ms, float rho, float (&L)[20])
+template <class T> __device__ __forceinline__ void m2l_side_a_forces_3(const T (&D)[20], const T *__restrict__ Ms, T rho, T (&L)[20])
 {
-    L[0] = 0.0f;
-    float rp = 1.0f;
-    { const float m = __ldg(Ms + 0) * rp;
+    L[0] = T(0);
+    T rp = T(1);
+    { const T m = __ldg(Ms + 0) * rp;
       L[1] = D[1] * m;
       L[2] = D[2] * m;
       L[3] = D[3] * m;
@@ -641,76 +649,76 @@ __device__ __forceinline__ void m2l_side_a_forces_3(const float (&D)[20], const 
       L[19] = D[19] * m;
     }
     rp *= rho;
-    { const float m = -__ldg(Ms + 1) * rp;
-      L[1] = fmaf(D[4], m, L[1]);
-      L[2] = fmaf(D[5], m, L[2]);
-      L[3] = fmaf(D[6], m, L[3]);
-      L[4] = fmaf(D[10], m, L[4]);
-      L[5] = fmaf(D[11], m, L[5]);
-      L[6] = fmaf(D[12], m, L[6]);
-      L[7] = fmaf(D[13], m, L[7]);
-      L[8] = fmaf(D[14], m, L[8]);
-      L[9] = fmaf(D[15], m, L[9]);
+    { const T m = -__ldg(Ms + 1) * rp;
+      L[1] = m2l_fma(D[4], m, L[1]);
+      L[2] = m2l_fma(D[5], m, L[2]);
+      L[3] = m2l_fma(D[6], m, L[3]);
+      L[4] = m2l_fma(D[10], m, L[4]);
+      L[5] = m2l_fma(D[11], m, L[5]);
+      L[6] = m2l_fma(D[12], m, L[6]);
+      L[7] = m2l_fma(D[13], m, L[7]);
+      L[8] = m2l_fma(D[14], m, L[8]);
+      L[9] = m2l_fma(D[15], m, L[9]);
     }
-    { const float m = -__ldg(Ms + 2) * rp;
-      L[1] = fmaf(D[5], m, L[1]);
-      L[2] = fmaf(D[7], m, L[2]);
-      L[3] = fmaf(D[8], m, L[3]);
-      L[4] = fmaf(D[11], m, L[4]);
-      L[5] = fmaf(D[13], m, L[5]);
-      L[6] = fmaf(D[14], m, L[6]);
-      L[7] = fmaf(D[16], m, L[7]);
-      L[8] = fmaf(D[17], m, L[8]);
-      L[9] = fmaf(D[18], m, L[9]);
+    { const T m = -__ldg(Ms + 2) * rp;
+      L[1] = m2l_fma(D[5], m, L[1]);
+      L[2] = m2l_fma(D[7], m, L[2]);
+      L[3] = m2l_fma(D[8], m, L[3]);
+      L[4] = m2l_fma(D[11], m, L[4]);
+      L[5] = m2l_fma(D[13], m, L[5]);
+      L[6] = m2l_fma(D[14], m, L[6]);
+      L[7] = m2l_fma(D[16], m, L[7]);
+      L[8] = m2l_fma(D[17], m, L[8]);
+      L[9] = m2l_fma(D[18], m, L[9]);
     }
-    { const float m = -__ldg(Ms + 3) * rp;
-      L[1] = fmaf(D[6], m, L[1]);
-      L[2] = fmaf(D[8], m, L[2]);
-      L[3] = fmaf(D[9], m, L[3]);
-      L[4] = fmaf(D[12], m, L[4]);
-      L[5] = fmaf(D[14], m, L[5]);
-      L[6] = fmaf(D[15], m, L[6]);
-      L[7] = fmaf(D[17], m, L[7]);
-      L[8] = fmaf(D[18], m, L[8]);
-      L[9] = fmaf(D[19], m, L[9]);
+    { const T m = -__ldg(Ms + 3) * rp;
+      L[1] = m2l_fma(D[6], m, L[1]);
+      L[2] = m2l_fma(D[8], m, L[2]);
+      L[3] = m2l_fma(D[9], m, L[3]);
+      L[4] = m2l_fma(D[12], m, L[4]);
+      L[5] = m2l_fma(D[14], m, L[5]);
+      L[6] = m2l_fma(D[15], m, L[6]);
+      L[7] = m2l_fma(D[17], m, L[7]);
+      L[8] = m2l_fma(D[18], m, L[8]);
+      L[9] = m2l_fma(D[19], m, L[9]);
     }
     rp *= rho;
-    { const float m = __ldg(Ms + 4) * rp;
-      L[1] = fmaf(D[10], m, L[1]);
-      L[2] = fmaf(D[11], m, L[2]);
-      L[3] = fmaf(D[12], m, L[3]);
+    { const T m = __ldg(Ms + 4) * rp;
+      L[1] = m2l_fma(D[10], m, L[1]);
+      L[2] = m2l_fma(D[11], m, L[2]);
+      L[3] = m2l_fma(D[12], m, L[3]);
     }
-    { const float m = __ldg(Ms + 5) * rp;
-      L[1] = fmaf(D[11], m, L[1]);
-      L[2] = fmaf(D[13], m, L[2]);
-      L[3] = fmaf(D[14], m, L[3]);
+    { const T m = __ldg(Ms + 5) * rp;
+      L[1] = m2l_fma(D[11], m, L[1]);
+      L[2] = m2l_fma(D[13], m, L[2]);
+      L[3] = m2l_fma(D[14], m, L[3]);
     }
-    { const float m = __ldg(Ms + 6) * rp;
-      L[1] = fmaf(D[12], m, L[1]);
-      L[2] = fmaf(D[14], m, L[2]);
-      L[3] = fmaf(D[15], m, L[3]);
+    { const T m = __ldg(Ms + 6) * rp;
+      L[1] = m2l_fma(D[12], m, L[1]);
+      L[2] = m2l_fma(D[14], m, L[2]);
+      L[3] = m2l_fma(D[15], m, L[3]);
     }
-    { const float m = __ldg(Ms + 7) * rp;
-      L[1] = fmaf(D[13], m, L[1]);
-      L[2] = fmaf(D[16], m, L[2]);
-      L[3] = fmaf(D[17], m, L[3]);
+    { const T m = __ldg(Ms + 7) * rp;
+      L[1] = m2l_fma(D[13], m, L[1]);
+      L[2] = m2l_fma(D[16], m, L[2]);
+      L[3] = m2l_fma(D[17], m, L[3]);
     }
-    { const float m = __ldg(Ms + 8) * rp;
-      L[1] = fmaf(D[14], m, L[1]);
-      L[2] = fmaf(D[17], m, L[2]);
-      L[3] = fmaf(D[18], m, L[3]);
+    { const T m = __ldg(Ms + 8) * rp;
+      L[1] = m2l_fma(D[14], m, L[1]);
+      L[2] = m2l_fma(D[17], m, L[2]);
+      L[3] = m2l_fma(D[18], m, L[3]);
     }
-    { const float m = __ldg(Ms + 9) * rp;
-      L[1] = fmaf(D[15], m, L[1]);
-      L[2] = fmaf(D[18], m, L[2]);
-      L[3] = fmaf(D[19], m, L[3]);
+    { const T m = __ldg(Ms + 9) * rp;
+      L[1] = m2l_fma(D[15], m, L[1]);
+      L[2] = m2l_fma(D[18], m, L[2]);
+      L[3] = m2l_fma(D[19], m, L[3]);
     }
 }
 
-__device__ __forceinline__ void m2l_side_b_forces_3(const float (&D)[20], const float *__restrict__ Ms, float (&L)[20])
+template <class T> __device__ __forceinline__ void m2l_side_b_forces_3(const T (&D)[20], const T *__restrict__ Ms, T (&L)[20])
 {
-    L[0] = 0.0f;
-    { const float m = __ldg(Ms + 0);
+    L[0] = T(0);
+    { const T m = __ldg(Ms + 0);
       L[1] = -D[1] * m;
       L[2] = -D[2] * m;
       L[3] = -D[3] * m;
@@ -731,152 +739,151 @@ __device__ __forceinline__ void m2l_side_b_forces_3(const float (&D)[20], const 
       L[18] = -D[18] * m;
       L[19] = -D[19] * m;
     }
-    { const float m = __ldg(Ms + 1);
-      L[1] = fmaf(-D[4], m, L[1]);
-      L[2] = fmaf(-D[5], m, L[2]);
-      L[3] = fmaf(-D[6], m, L[3]);
-      L[4] = fmaf(D[10], m, L[4]);
-      L[5] = fmaf(D[11], m, L[5]);
-      L[6] = fmaf(D[12], m, L[6]);
-      L[7] = fmaf(D[13], m, L[7]);
-      L[8] = fmaf(D[14], m, L[8]);
-      L[9] = fmaf(D[15], m, L[9]);
+    { const T m = __ldg(Ms + 1);
+      L[1] = m2l_fma(-D[4], m, L[1]);
+      L[2] = m2l_fma(-D[5], m, L[2]);
+      L[3] = m2l_fma(-D[6], m, L[3]);
+      L[4] = m2l_fma(D[10], m, L[4]);
+      L[5] = m2l_fma(D[11], m, L[5]);
+      L[6] = m2l_fma(D[12], m, L[6]);
+      L[7] = m2l_fma(D[13], m, L[7]);
+      L[8] = m2l_fma(D[14], m, L[8]);
+      L[9] = m2l_fma(D[15], m, L[9]);
     }
-    { const float m = __ldg(Ms + 2);
-      L[1] = fmaf(-D[5], m, L[1]);
-      L[2] = fmaf(-D[7], m, L[2]);
-      L[3] = fmaf(-D[8], m, L[3]);
-      L[4] = fmaf(D[11], m, L[4]);
-      L[5] = fmaf(D[13], m, L[5]);
-      L[6] = fmaf(D[14], m, L[6]);
-      L[7] = fmaf(D[16], m, L[7]);
-      L[8] = fmaf(D[17], m, L[8]);
-      L[9] = fmaf(D[18], m, L[9]);
+    { const T m = __ldg(Ms + 2);
+      L[1] = m2l_fma(-D[5], m, L[1]);
+      L[2] = m2l_fma(-D[7], m, L[2]);
+      L[3] = m2l_fma(-D[8], m, L[3]);
+      L[4] = m2l_fma(D[11], m, L[4]);
+      L[5] = m2l_fma(D[13], m, L[5]);
+      L[6] = m2l_fma(D[14], m, L[6]);
+      L[7] = m2l_fma(D[16], m, L[7]);
+      L[8] = m2l_fma(D[17], m, L[8]);
+      L[9] = m2l_fma(D[18], m, L[9]);
     }
-    { const float m = __ldg(Ms + 3);
-      L[1] = fmaf(-D[6], m, L[1]);
-      L[2] = fmaf(-D[8], m, L[2]);
-      L[3] = fmaf(-D[9], m, L[3]);
-      L[4] = fmaf(D[12], m, L[4]);
-      L[5] = fmaf(D[14], m, L[5]);
-      L[6] = fmaf(D[15], m, L[6]);
-      L[7] = fmaf(D[17], m, L[7]);
-      L[8] = fmaf(D[18], m, L[8]);
-      L[9] = fmaf(D[19], m, L[9]);
+    { const T m = __ldg(Ms + 3);
+      L[1] = m2l_fma(-D[6], m, L[1]);
+      L[2] = m2l_fma(-D[8], m, L[2]);
+      L[3] = m2l_fma(-D[9], m, L[3]);
+      L[4] = m2l_fma(D[12], m, L[4]);
+      L[5] = m2l_fma(D[14], m, L[5]);
+      L[6] = m2l_fma(D[15], m, L[6]);
+      L[7] = m2l_fma(D[17], m, L[7]);
+      L[8] = m2l_fma(D[18], m, L[8]);
+      L[9] = m2l_fma(D[19], m, L[9]);
     }
-    { const float m = __ldg(Ms + 4);
-      L[1] = fmaf(-D[10], m, L[1]);
-      L[2] = fmaf(-D[11], m, L[2]);
-      L[3] = fmaf(-D[12], m, L[3]);
+    { const T m = __ldg(Ms + 4);
+      L[1] = m2l_fma(-D[10], m, L[1]);
+      L[2] = m2l_fma(-D[11], m, L[2]);
+      L[3] = m2l_fma(-D[12], m, L[3]);
     }
-    { const float m = __ldg(Ms + 5);
-      L[1] = fmaf(-D[11], m, L[1]);
-      L[2] = fmaf(-D[13], m, L[2]);
-      L[3] = fmaf(-D[14], m, L[3]);
+    { const T m = __ldg(Ms + 5);
+      L[1] = m2l_fma(-D[11], m, L[1]);
+      L[2] = m2l_fma(-D[13], m, L[2]);
+      L[3] = m2l_fma(-D[14], m, L[3]);
     }
-    { const float m = __ldg(Ms + 6);
-      L[1] = fmaf(-D[12], m, L[1]);
-      L[2] = fmaf(-D[14], m, L[2]);
-      L[3] = fmaf(-D[15], m, L[3]);
+    { const T m = __ldg(Ms + 6);
+      L[1] = m2l_fma(-D[12], m, L[1]);
+      L[2] = m2l_fma(-D[14], m, L[2]);
+      L[3] = m2l_fma(-D[15], m, L[3]);
     }
-    { const float m = __ldg(Ms + 7);
-      L[1] = fmaf(-D[13], m, L[1]);
-      L[2] = fmaf(-D[16], m, L[2]);
-      L[3] = fmaf(-D[17], m, L[3]);
+    { const T m = __ldg(Ms + 7);
+      L[1] = m2l_fma(-D[13], m, L[1]);
+      L[2] = m2l_fma(-D[16], m, L[2]);
+      L[3] = m2l_fma(-D[17], m, L[3]);
     }
-    { const float m = __ldg(Ms + 8);
-      L[1] = fmaf(-D[14], m, L[1]);
-      L[2] = fmaf(-D[17], m, L[2]);
-      L[3] = fmaf(-D[18], m, L[3]);
+    { const T m = __ldg(Ms + 8);
+      L[1] = m2l_fma(-D[14], m, L[1]);
+      L[2] = m2l_fma(-D[17], m, L[2]);
+      L[3] = m2l_fma(-D[18], m, L[3]);
     }
-    { const float m = __ldg(Ms + 9);
-      L[1] = fmaf(-D[15], m, L[1]);
-      L[2] = fmaf(-D[18], m, L[2]);
-      L[3] = fmaf(-D[19], m, L[3]);
+    { const T m = __ldg(Ms + 9);
+      L[1] = m2l_fma(-D[15], m, L[1]);
+      L[2] = m2l_fma(-D[18], m, L[2]);
+      L[3] = m2l_fma(-D[19], m, L[3]);
     }
 }
 
-__device__ __forceinline__ void m2l_dtensor_4(float dx, float dy, float dz, float soft2, float (&D)[35])
+template <class T> __device__ __forceinline__ void m2l_dtensor_4(T dx, T dy, T dz, T soft2, T (&D)[35])
 {
-    const float s2 = fmaf(dx, dx, fmaf(dy, dy, fmaf(dz, dz, soft2)));
-    float si = rsqrtf(s2);
-    si = si * fmaf(-0.5f * s2, si * si, 1.5f);   // one Newton step
-    const float si2 = si * si;
-    const float f0 = -si;
-    const float f1 = -1.0f * f0 * si2;
-    const float f2 = -3.0f * f1 * si2;
-    const float f3 = -5.0f * f2 * si2;
-    const float f4 = -7.0f * f3 * si2;
-    const float r_0_0 = f0;
-    const float r_1_0 = f1;
-    const float r_2_0 = f2;
-    const float r_3_0 = f3;
-    const float r_4_0 = f4;
-    const float r_0_1 = dx * r_1_0;
-    const float r_1_1 = dx * r_2_0;
-    const float r_2_1 = dx * r_3_0;
-    const float r_3_1 = dx * r_4_0;
-    const float r_0_2 = dy * r_1_0;
-    const float r_1_2 = dy * r_2_0;
-    const float r_2_2 = dy * r_3_0;
-    const float r_3_2 = dy * r_4_0;
-    const float r_0_3 = dz * r_1_0;
-    const float r_1_3 = dz * r_2_0;
-    const float r_2_3 = dz * r_3_0;
-    const float r_3_3 = dz * r_4_0;
-    const float r_0_4 = fmaf(1.0f, r_1_0, dx * r_1_1);
-    const float r_1_4 = fmaf(1.0f, r_2_0, dx * r_2_1);
-    const float r_2_4 = fmaf(1.0f, r_3_0, dx * r_3_1);
-    const float r_0_5 = dx * r_1_2;
-    const float r_1_5 = dx * r_2_2;
-    const float r_2_5 = dx * r_3_2;
-    const float r_0_6 = dx * r_1_3;
-    const float r_1_6 = dx * r_2_3;
-    const float r_2_6 = dx * r_3_3;
-    const float r_0_7 = fmaf(1.0f, r_1_0, dy * r_1_2);
-    const float r_1_7 = fmaf(1.0f, r_2_0, dy * r_2_2);
-    const float r_2_7 = fmaf(1.0f, r_3_0, dy * r_3_2);
-    const float r_0_8 = dy * r_1_3;
-    const float r_1_8 = dy * r_2_3;
-    const float r_2_8 = dy * r_3_3;
-    const float r_0_9 = fmaf(1.0f, r_1_0, dz * r_1_3);
-    const float r_1_9 = fmaf(1.0f, r_2_0, dz * r_2_3);
-    const float r_2_9 = fmaf(1.0f, r_3_0, dz * r_3_3);
-    const float r_0_10 = fmaf(2.0f, r_1_1, dx * r_1_4);
-    const float r_1_10 = fmaf(2.0f, r_2_1, dx * r_2_4);
-    const float r_0_11 = fmaf(1.0f, r_1_2, dx * r_1_5);
-    const float r_1_11 = fmaf(1.0f, r_2_2, dx * r_2_5);
-    const float r_0_12 = fmaf(1.0f, r_1_3, dx * r_1_6);
-    const float r_1_12 = fmaf(1.0f, r_2_3, dx * r_2_6);
-    const float r_0_13 = dx * r_1_7;
-    const float r_1_13 = dx * r_2_7;
-    const float r_0_14 = dx * r_1_8;
-    const float r_1_14 = dx * r_2_8;
-    const float r_0_15 = dx * r_1_9;
-    const float r_1_15 = dx * r_2_9;
-    const float r_0_16 = fmaf(2.0f, r_1_2, dy * r_1_7);
-    const float r_1_16 = fmaf(2.0f, r_2_2, dy * r_2_7);
-    const float r_0_17 = fmaf(1.0f, r_1_3, dy * r_1_8);
-    const float r_1_17 = fmaf(1.0f, r_2_3, dy * r_2_8);
-    const float r_0_18 = dy * r_1_9;
-    const float r_1_18 = dy * r_2_9;
-    const float r_0_19 = fmaf(2.0f, r_1_3, dz * r_1_9);
-    const float r_1_19 = fmaf(2.0f, r_2_3, dz * r_2_9);
-    const float r_0_20 = fmaf(3.0f, r_1_4, dx * r_1_10);
-    const float r_0_21 = fmaf(2.0f, r_1_5, dx * r_1_11);
-    const float r_0_22 = fmaf(2.0f, r_1_6, dx * r_1_12);
-    const float r_0_23 = fmaf(1.0f, r_1_7, dx * r_1_13);
-    const float r_0_24 = fmaf(1.0f, r_1_8, dx * r_1_14);
-    const float r_0_25 = fmaf(1.0f, r_1_9, dx * r_1_15);
-    const float r_0_26 = dx * r_1_16;
-    const float r_0_27 = dx * r_1_17;
-    const float r_0_28 = dx * r_1_18;
-    const float r_0_29 = dx * r_1_19;
-    const float r_0_30 = fmaf(3.0f, r_1_7, dy * r_1_16);
-    const float r_0_31 = fmaf(2.0f, r_1_8, dy * r_1_17);
-    const float r_0_32 = fmaf(1.0f, r_1_9, dy * r_1_18);
-    const float r_0_33 = dy * r_1_19;
-    const float r_0_34 = fmaf(3.0f, r_1_9, dz * r_1_19);
+    const T s2 = m2l_fma(dx, dx, m2l_fma(dy, dy, m2l_fma(dz, dz, soft2)));
+    const T si = m2l_rsqrt(s2);
+    const T si2 = si * si;
+    const T f0 = -si;
+    const T f1 = T(-1) * f0 * si2;
+    const T f2 = T(-3) * f1 * si2;
+    const T f3 = T(-5) * f2 * si2;
+    const T f4 = T(-7) * f3 * si2;
+    const T r_0_0 = f0;
+    const T r_1_0 = f1;
+    const T r_2_0 = f2;
+    const T r_3_0 = f3;
+    const T r_4_0 = f4;
+    const T r_0_1 = dx * r_1_0;
+    const T r_1_1 = dx * r_2_0;
+    const T r_2_1 = dx * r_3_0;
+    const T r_3_1 = dx * r_4_0;
+    const T r_0_2 = dy * r_1_0;
+    const T r_1_2 = dy * r_2_0;
+    const T r_2_2 = dy * r_3_0;
+    const T r_3_2 = dy * r_4_0;
+    const T r_0_3 = dz * r_1_0;
+    const T r_1_3 = dz * r_2_0;
+    const T r_2_3 = dz * r_3_0;
+    const T r_3_3 = dz * r_4_0;
+    const T r_0_4 = m2l_fma(T(1), r_1_0, dx * r_1_1);
+    const T r_1_4 = m2l_fma(T(1), r_2_0, dx * r_2_1);
+    const T r_2_4 = m2l_fma(T(1), r_3_0, dx * r_3_1);
+    const T r_0_5 = dx * r_1_2;
+    const T r_1_5 = dx * r_2_2;
+    const T r_2_5 = dx * r_3_2;
+    const T r_0_6 = dx * r_1_3;
+    const T r_1_6 = dx * r_2_3;
+    const T r_2_6 = dx * r_3_3;
+    const T r_0_7 = m2l_fma(T(1), r_1_0, dy * r_1_2);
+    const T r_1_7 = m2l_fma(T(1), r_2_0, dy * r_2_2);
+    const T r_2_7 = m2l_fma(T(1), r_3_0, dy * r_3_2);
+    const T r_0_8 = dy * r_1_3;
+    const T r_1_8 = dy * r_2_3;
+    const T r_2_8 = dy * r_3_3;
+    const T r_0_9 = m2l_fma(T(1), r_1_0, dz * r_1_3);
+    const T r_1_9 = m2l_fma(T(1), r_2_0, dz * r_2_3);
+    const T r_2_9 = m2l_fma(T(1), r_3_0, dz * r_3_3);
+    const T r_0_10 = m2l_fma(T(2), r_1_1, dx * r_1_4);
+    const T r_1_10 = m2l_fma(T(2), r_2_1, dx * r_2_4);
+    const T r_0_11 = m2l_fma(T(1), r_1_2, dx * r_1_5);
+    const T r_1_11 = m2l_fma(T(1), r_2_2, dx * r_2_5);
+    const T r_0_12 = m2l_fma(T(1), r_1_3, dx * r_1_6);
+    const T r_1_12 = m2l_fma(T(1), r_2_3, dx * r_2_6);
+    const T r_0_13 = dx * r_1_7;
+    const T r_1_13 = dx * r_2_7;
+    const T r_0_14 = dx * r_1_8;
+    const T r_1_14 = dx * r_2_8;
+    const T r_0_15 = dx * r_1_9;
+    const T r_1_15 = dx * r_2_9;
+    const T r_0_16 = m2l_fma(T(2), r_1_2, dy * r_1_7);
+    const T r_1_16 = m2l_fma(T(2), r_2_2, dy * r_2_7);
+    const T r_0_17 = m2l_fma(T(1), r_1_3, dy * r_1_8);
+    const T r_1_17 = m2l_fma(T(1), r_2_3, dy * r_2_8);
+    const T r_0_18 = dy * r_1_9;
+    const T r_1_18 = dy * r_2_9;
+    const T r_0_19 = m2l_fma(T(2), r_1_3, dz * r_1_9);
+    const T r_1_19 = m2l_fma(T(2), r_2_3, dz * r_2_9);
+    const T r_0_20 = m2l_fma(T(3), r_1_4, dx * r_1_10);
+    const T r_0_21 = m2l_fma(T(2), r_1_5, dx * r_1_11);
+    const T r_0_22 = m2l_fma(T(2), r_1_6, dx * r_1_12);
+    const T r_0_23 = m2l_fma(T(1), r_1_7, dx * r_1_13);
+    const T r_0_24 = m2l_fma(T(1), r_1_8, dx * r_1_14);
+    const T r_0_25 = m2l_fma(T(1), r_1_9, dx * r_1_15);
+    const T r_0_26 = dx * r_1_16;
+    const T r_0_27 = dx * r_1_17;
+    const T r_0_28 = dx * r_1_18;
+    const T r_0_29 = dx * r_1_19;
+    const T r_0_30 = m2l_fma(T(3), r_1_7, dy * r_1_16);
+    const T r_0_31 = m2l_fma(T(2), r_1_8, dy * r_1_17);
+    const T r_0_32 = m2l_fma(T(1), r_1_9, dy * r_1_18);
+    const T r_0_33 = dy * r_1_19;
+    const T r_0_34 = m2l_fma(T(3), r_1_9, dz * r_1_19);
     D[0] = r_0_0;
     D[1] = r_0_1;
     D[2] = r_0_2;
@@ -914,10 +921,10 @@ __device__ __forceinline__ void m2l_dtensor_4(float dx, float dy, float dz, floa
     D[34] = r_0_34;
 }
 
-__device__ __forceinline__ void m2l_side_a_4(const float (&D)[35], const float *__restrict__ Ms, float rho, float (&L)[35])
+template <class T> __device__ __forceinline__ void m2l_side_a_4(const T (&D)[35], const T *__restrict__ Ms, T rho, T (&L)[35])
 {
-    float rp = 1.0f;
-    { const float m = __ldg(Ms + 0) * rp;
+    T rp = T(1);
+    { const T m = __ldg(Ms + 0) * rp;
       L[0] = D[0] * m;
       L[1] = D[1] * m;
       L[2] = D[2] * m;
@@ -955,257 +962,257 @@ __device__ __forceinline__ void m2l_side_a_4(const float (&D)[35], const float *
       L[34] = D[34] * m;
     }
     rp *= rho;
-    { const float m = -__ldg(Ms + 1) * rp;
-      L[0] = fmaf(D[1], m, L[0]);
-      L[1] = fmaf(D[4], m, L[1]);
-      L[2] = fmaf(D[5], m, L[2]);
-      L[3] = fmaf(D[6], m, L[3]);
-      L[4] = fmaf(D[10], m, L[4]);
-      L[5] = fmaf(D[11], m, L[5]);
-      L[6] = fmaf(D[12], m, L[6]);
-      L[7] = fmaf(D[13], m, L[7]);
-      L[8] = fmaf(D[14], m, L[8]);
-      L[9] = fmaf(D[15], m, L[9]);
-      L[10] = fmaf(D[20], m, L[10]);
-      L[11] = fmaf(D[21], m, L[11]);
-      L[12] = fmaf(D[22], m, L[12]);
-      L[13] = fmaf(D[23], m, L[13]);
-      L[14] = fmaf(D[24], m, L[14]);
-      L[15] = fmaf(D[25], m, L[15]);
-      L[16] = fmaf(D[26], m, L[16]);
-      L[17] = fmaf(D[27], m, L[17]);
-      L[18] = fmaf(D[28], m, L[18]);
-      L[19] = fmaf(D[29], m, L[19]);
+    { const T m = -__ldg(Ms + 1) * rp;
+      L[0] = m2l_fma(D[1], m, L[0]);
+      L[1] = m2l_fma(D[4], m, L[1]);
+      L[2] = m2l_fma(D[5], m, L[2]);
+      L[3] = m2l_fma(D[6], m, L[3]);
+      L[4] = m2l_fma(D[10], m, L[4]);
+      L[5] = m2l_fma(D[11], m, L[5]);
+      L[6] = m2l_fma(D[12], m, L[6]);
+      L[7] = m2l_fma(D[13], m, L[7]);
+      L[8] = m2l_fma(D[14], m, L[8]);
+      L[9] = m2l_fma(D[15], m, L[9]);
+      L[10] = m2l_fma(D[20], m, L[10]);
+      L[11] = m2l_fma(D[21], m, L[11]);
+      L[12] = m2l_fma(D[22], m, L[12]);
+      L[13] = m2l_fma(D[23], m, L[13]);
+      L[14] = m2l_fma(D[24], m, L[14]);
+      L[15] = m2l_fma(D[25], m, L[15]);
+      L[16] = m2l_fma(D[26], m, L[16]);
+      L[17] = m2l_fma(D[27], m, L[17]);
+      L[18] = m2l_fma(D[28], m, L[18]);
+      L[19] = m2l_fma(D[29], m, L[19]);
     }
-    { const float m = -__ldg(Ms + 2) * rp;
-      L[0] = fmaf(D[2], m, L[0]);
-      L[1] = fmaf(D[5], m, L[1]);
-      L[2] = fmaf(D[7], m, L[2]);
-      L[3] = fmaf(D[8], m, L[3]);
-      L[4] = fmaf(D[11], m, L[4]);
-      L[5] = fmaf(D[13], m, L[5]);
-      L[6] = fmaf(D[14], m, L[6]);
-      L[7] = fmaf(D[16], m, L[7]);
-      L[8] = fmaf(D[17], m, L[8]);
-      L[9] = fmaf(D[18], m, L[9]);
-      L[10] = fmaf(D[21], m, L[10]);
-      L[11] = fmaf(D[23], m, L[11]);
-      L[12] = fmaf(D[24], m, L[12]);
-      L[13] = fmaf(D[26], m, L[13]);
-      L[14] = fmaf(D[27], m, L[14]);
-      L[15] = fmaf(D[28], m, L[15]);
-      L[16] = fmaf(D[30], m, L[16]);
-      L[17] = fmaf(D[31], m, L[17]);
-      L[18] = fmaf(D[32], m, L[18]);
-      L[19] = fmaf(D[33], m, L[19]);
+    { const T m = -__ldg(Ms + 2) * rp;
+      L[0] = m2l_fma(D[2], m, L[0]);
+      L[1] = m2l_fma(D[5], m, L[1]);
+      L[2] = m2l_fma(D[7], m, L[2]);
+      L[3] = m2l_fma(D[8], m, L[3]);
+      L[4] = m2l_fma(D[11], m, L[4]);
+      L[5] = m2l_fma(D[13], m, L[5]);
+      L[6] = m2l_fma(D[14], m, L[6]);
+      L[7] = m2l_fma(D[16], m, L[7]);
+      L[8] = m2l_fma(D[17], m, L[8]);
+      L[9] = m2l_fma(D[18], m, L[9]);
+      L[10] = m2l_fma(D[21], m, L[10]);
+      L[11] = m2l_fma(D[23], m, L[11]);
+      L[12] = m2l_fma(D[24], m, L[12]);
+      L[13] = m2l_fma(D[26], m, L[13]);
+      L[14] = m2l_fma(D[27], m, L[14]);
+      L[15] = m2l_fma(D[28], m, L[15]);
+      L[16] = m2l_fma(D[30], m, L[16]);
+      L[17] = m2l_fma(D[31], m, L[17]);
+      L[18] = m2l_fma(D[32], m, L[18]);
+      L[19] = m2l_fma(D[33], m, L[19]);
     }
-    { const float m = -__ldg(Ms + 3) * rp;
-      L[0] = fmaf(D[3], m, L[0]);
-      L[1] = fmaf(D[6], m, L[1]);
-      L[2] = fmaf(D[8], m, L[2]);
-      L[3] = fmaf(D[9], m, L[3]);
-      L[4] = fmaf(D[12], m, L[4]);
-      L[5] = fmaf(D[14], m, L[5]);
-      L[6] = fmaf(D[15], m, L[6]);
-      L[7] = fmaf(D[17], m, L[7]);
-      L[8] = fmaf(D[18], m, L[8]);
-      L[9] = fmaf(D[19], m, L[9]);
-      L[10] = fmaf(D[22], m, L[10]);
-      L[11] = fmaf(D[24], m, L[11]);
-      L[12] = fmaf(D[25], m, L[12]);
-      L[13] = fmaf(D[27], m, L[13]);
-      L[14] = fmaf(D[28], m, L[14]);
-      L[15] = fmaf(D[29], m, L[15]);
-      L[16] = fmaf(D[31], m, L[16]);
-      L[17] = fmaf(D[32], m, L[17]);
-      L[18] = fmaf(D[33], m, L[18]);
-      L[19] = fmaf(D[34], m, L[19]);
-    }
-    rp *= rho;
-    { const float m = __ldg(Ms + 4) * rp;
-      L[0] = fmaf(D[4], m, L[0]);
-      L[1] = fmaf(D[10], m, L[1]);
-      L[2] = fmaf(D[11], m, L[2]);
-      L[3] = fmaf(D[12], m, L[3]);
-      L[4] = fmaf(D[20], m, L[4]);
-      L[5] = fmaf(D[21], m, L[5]);
-      L[6] = fmaf(D[22], m, L[6]);
-      L[7] = fmaf(D[23], m, L[7]);
-      L[8] = fmaf(D[24], m, L[8]);
-      L[9] = fmaf(D[25], m, L[9]);
-    }
-    { const float m = __ldg(Ms + 5) * rp;
-      L[0] = fmaf(D[5], m, L[0]);
-      L[1] = fmaf(D[11], m, L[1]);
-      L[2] = fmaf(D[13], m, L[2]);
-      L[3] = fmaf(D[14], m, L[3]);
-      L[4] = fmaf(D[21], m, L[4]);
-      L[5] = fmaf(D[23], m, L[5]);
-      L[6] = fmaf(D[24], m, L[6]);
-      L[7] = fmaf(D[26], m, L[7]);
-      L[8] = fmaf(D[27], m, L[8]);
-      L[9] = fmaf(D[28], m, L[9]);
-    }
-    { const float m = __ldg(Ms + 6) * rp;
-      L[0] = fmaf(D[6], m, L[0]);
-      L[1] = fmaf(D[12], m, L[1]);
-      L[2] = fmaf(D[14], m, L[2]);
-      L[3] = fmaf(D[15], m, L[3]);
-      L[4] = fmaf(D[22], m, L[4]);
-      L[5] = fmaf(D[24], m, L[5]);
-      L[6] = fmaf(D[25], m, L[6]);
-      L[7] = fmaf(D[27], m, L[7]);
-      L[8] = fmaf(D[28], m, L[8]);
-      L[9] = fmaf(D[29], m, L[9]);
-    }
-    { const float m = __ldg(Ms + 7) * rp;
-      L[0] = fmaf(D[7], m, L[0]);
-      L[1] = fmaf(D[13], m, L[1]);
-      L[2] = fmaf(D[16], m, L[2]);
-      L[3] = fmaf(D[17], m, L[3]);
-      L[4] = fmaf(D[23], m, L[4]);
-      L[5] = fmaf(D[26], m, L[5]);
-      L[6] = fmaf(D[27], m, L[6]);
-      L[7] = fmaf(D[30], m, L[7]);
-      L[8] = fmaf(D[31], m, L[8]);
-      L[9] = fmaf(D[32], m, L[9]);
-    }
-    { const float m = __ldg(Ms + 8) * rp;
-      L[0] = fmaf(D[8], m, L[0]);
-      L[1] = fmaf(D[14], m, L[1]);
-      L[2] = fmaf(D[17], m, L[2]);
-      L[3] = fmaf(D[18], m, L[3]);
-      L[4] = fmaf(D[24], m, L[4]);
-      L[5] = fmaf(D[27], m, L[5]);
-      L[6] = fmaf(D[28], m, L[6]);
-      L[7] = fmaf(D[31], m, L[7]);
-      L[8] = fmaf(D[32], m, L[8]);
-      L[9] = fmaf(D[33], m, L[9]);
-    }
-    { const float m = __ldg(Ms + 9) * rp;
-      L[0] = fmaf(D[9], m, L[0]);
-      L[1] = fmaf(D[15], m, L[1]);
-      L[2] = fmaf(D[18], m, L[2]);
-      L[3] = fmaf(D[19], m, L[3]);
-      L[4] = fmaf(D[25], m, L[4]);
-      L[5] = fmaf(D[28], m, L[5]);
-      L[6] = fmaf(D[29], m, L[6]);
-      L[7] = fmaf(D[32], m, L[7]);
-      L[8] = fmaf(D[33], m, L[8]);
-      L[9] = fmaf(D[34], m, L[9]);
+    { const T m = -__ldg(Ms + 3) * rp;
+      L[0] = m2l_fma(D[3], m, L[0]);
+      L[1] = m2l_fma(D[6], m, L[1]);
+      L[2] = m2l_fma(D[8], m, L[2]);
+      L[3] = m2l_fma(D[9], m, L[3]);
+      L[4] = m2l_fma(D[12], m, L[4]);
+      L[5] = m2l_fma(D[14], m, L[5]);
+      L[6] = m2l_fma(D[15], m, L[6]);
+      L[7] = m2l_fma(D[17], m, L[7]);
+      L[8] = m2l_fma(D[18], m, L[8]);
+      L[9] = m2l_fma(D[19], m, L[9]);
+      L[10] = m2l_fma(D[22], m, L[10]);
+      L[11] = m2l_fma(D[24], m, L[11]);
+      L[12] = m2l_fma(D[25], m, L[12]);
+      L[13] = m2l_fma(D[27], m, L[13]);
+      L[14] = m2l_fma(D[28], m, L[14]);
+      L[15] = m2l_fma(D[29], m, L[15]);
+      L[16] = m2l_fma(D[31], m, L[16]);
+      L[17] = m2l_fma(D[32], m, L[17]);
+      L[18] = m2l_fma(D[33], m, L[18]);
+      L[19] = m2l_fma(D[34], m, L[19]);
     }
     rp *= rho;
-    { const float m = -__ldg(Ms + 10) * rp;
-      L[0] = fmaf(D[10], m, L[0]);
-      L[1] = fmaf(D[20], m, L[1]);
-      L[2] = fmaf(D[21], m, L[2]);
-      L[3] = fmaf(D[22], m, L[3]);
+    { const T m = __ldg(Ms + 4) * rp;
+      L[0] = m2l_fma(D[4], m, L[0]);
+      L[1] = m2l_fma(D[10], m, L[1]);
+      L[2] = m2l_fma(D[11], m, L[2]);
+      L[3] = m2l_fma(D[12], m, L[3]);
+      L[4] = m2l_fma(D[20], m, L[4]);
+      L[5] = m2l_fma(D[21], m, L[5]);
+      L[6] = m2l_fma(D[22], m, L[6]);
+      L[7] = m2l_fma(D[23], m, L[7]);
+      L[8] = m2l_fma(D[24], m, L[8]);
+      L[9] = m2l_fma(D[25], m, L[9]);
     }
-    { const float m = -__ldg(Ms + 11) * rp;
-      L[0] = fmaf(D[11], m, L[0]);
-      L[1] = fmaf(D[21], m, L[1]);
-      L[2] = fmaf(D[23], m, L[2]);
-      L[3] = fmaf(D[24], m, L[3]);
+    { const T m = __ldg(Ms + 5) * rp;
+      L[0] = m2l_fma(D[5], m, L[0]);
+      L[1] = m2l_fma(D[11], m, L[1]);
+      L[2] = m2l_fma(D[13], m, L[2]);
+      L[3] = m2l_fma(D[14], m, L[3]);
+      L[4] = m2l_fma(D[21], m, L[4]);
+      L[5] = m2l_fma(D[23], m, L[5]);
+      L[6] = m2l_fma(D[24], m, L[6]);
+      L[7] = m2l_fma(D[26], m, L[7]);
+      L[8] = m2l_fma(D[27], m, L[8]);
+      L[9] = m2l_fma(D[28], m, L[9]);
     }
-    { const float m = -__ldg(Ms + 12) * rp;
-      L[0] = fmaf(D[12], m, L[0]);
-      L[1] = fmaf(D[22], m, L[1]);
-      L[2] = fmaf(D[24], m, L[2]);
-      L[3] = fmaf(D[25], m, L[3]);
+    { const T m = __ldg(Ms + 6) * rp;
+      L[0] = m2l_fma(D[6], m, L[0]);
+      L[1] = m2l_fma(D[12], m, L[1]);
+      L[2] = m2l_fma(D[14], m, L[2]);
+      L[3] = m2l_fma(D[15], m, L[3]);
+      L[4] = m2l_fma(D[22], m, L[4]);
+      L[5] = m2l_fma(D[24], m, L[5]);
+      L[6] = m2l_fma(D[25], m, L[6]);
+      L[7] = m2l_fma(D[27], m, L[7]);
+      L[8] = m2l_fma(D[28], m, L[8]);
+      L[9] = m2l_fma(D[29], m, L[9]);
     }
-    { const float m = -__ldg(Ms + 13) * rp;
-      L[0] = fmaf(D[13], m, L[0]);
-      L[1] = fmaf(D[23], m, L[1]);
-      L[2] = fmaf(D[26], m, L[2]);
-      L[3] = fmaf(D[27], m, L[3]);
+    { const T m = __ldg(Ms + 7) * rp;
+      L[0] = m2l_fma(D[7], m, L[0]);
+      L[1] = m2l_fma(D[13], m, L[1]);
+      L[2] = m2l_fma(D[16], m, L[2]);
+      L[3] = m2l_fma(D[17], m, L[3]);
+      L[4] = m2l_fma(D[23], m, L[4]);
+      L[5] = m2l_fma(D[26], m, L[5]);
+      L[6] = m2l_fma(D[27], m, L[6]);
+      L[7] = m2l_fma(D[30], m, L[7]);
+      L[8] = m2l_fma(D[31], m, L[8]);
+      L[9] = m2l_fma(D[32], m, L[9]);
     }
-    { const float m = -__ldg(Ms + 14) * rp;
-      L[0] = fmaf(D[14], m, L[0]);
-      L[1] = fmaf(D[24], m, L[1]);
-      L[2] = fmaf(D[27], m, L[2]);
-      L[3] = fmaf(D[28], m, L[3]);
+    { const T m = __ldg(Ms + 8) * rp;
+      L[0] = m2l_fma(D[8], m, L[0]);
+      L[1] = m2l_fma(D[14], m, L[1]);
+      L[2] = m2l_fma(D[17], m, L[2]);
+      L[3] = m2l_fma(D[18], m, L[3]);
+      L[4] = m2l_fma(D[24], m, L[4]);
+      L[5] = m2l_fma(D[27], m, L[5]);
+      L[6] = m2l_fma(D[28], m, L[6]);
+      L[7] = m2l_fma(D[31], m, L[7]);
+      L[8] = m2l_fma(D[32], m, L[8]);
+      L[9] = m2l_fma(D[33], m, L[9]);
     }
-    { const float m = -__ldg(Ms + 15) * rp;
-      L[0] = fmaf(D[15], m, L[0]);
-      L[1] = fmaf(D[25], m, L[1]);
-      L[2] = fmaf(D[28], m, L[2]);
-      L[3] = fmaf(D[29], m, L[3]);
-    }
-    { const float m = -__ldg(Ms + 16) * rp;
-      L[0] = fmaf(D[16], m, L[0]);
-      L[1] = fmaf(D[26], m, L[1]);
-      L[2] = fmaf(D[30], m, L[2]);
-      L[3] = fmaf(D[31], m, L[3]);
-    }
-    { const float m = -__ldg(Ms + 17) * rp;
-      L[0] = fmaf(D[17], m, L[0]);
-      L[1] = fmaf(D[27], m, L[1]);
-      L[2] = fmaf(D[31], m, L[2]);
-      L[3] = fmaf(D[32], m, L[3]);
-    }
-    { const float m = -__ldg(Ms + 18) * rp;
-      L[0] = fmaf(D[18], m, L[0]);
-      L[1] = fmaf(D[28], m, L[1]);
-      L[2] = fmaf(D[32], m, L[2]);
-      L[3] = fmaf(D[33], m, L[3]);
-    }
-    { const float m = -__ldg(Ms + 19) * rp;
-      L[0] = fmaf(D[19], m, L[0]);
-      L[1] = fmaf(D[29], m, L[1]);
-      L[2] = fmaf(D[33], m, L[2]);
-      L[3] = fmaf(D[34], m, L[3]);
+    { const T m = __ldg(Ms + 9) * rp;
+      L[0] = m2l_fma(D[9], m, L[0]);
+      L[1] = m2l_fma(D[15], m, L[1]);
+      L[2] = m2l_fma(D[18], m, L[2]);
+      L[3] = m2l_fma(D[19], m, L[3]);
+      L[4] = m2l_fma(D[25], m, L[4]);
+      L[5] = m2l_fma(D[28], m, L[5]);
+      L[6] = m2l_fma(D[29], m, L[6]);
+      L[7] = m2l_fma(D[32], m, L[7]);
+      L[8] = m2l_fma(D[33], m, L[8]);
+      L[9] = m2l_fma(D[34], m, L[9]);
     }
     rp *= rho;
-    { const float m = __ldg(Ms + 20) * rp;
-      L[0] = fmaf(D[20], m, L[0]);
+    { const T m = -__ldg(Ms + 10) * rp;
+      L[0] = m2l_fma(D[10], m, L[0]);
+      L[1] = m2l_fma(D[20], m, L[1]);
+      L[2] = m2l_fma(D[21], m, L[2]);
+      L[3] = m2l_fma(D[22], m, L[3]);
     }
-    { const float m = __ldg(Ms + 21) * rp;
-      L[0] = fmaf(D[21], m, L[0]);
+    { const T m = -__ldg(Ms + 11) * rp;
+      L[0] = m2l_fma(D[11], m, L[0]);
+      L[1] = m2l_fma(D[21], m, L[1]);
+      L[2] = m2l_fma(D[23], m, L[2]);
+      L[3] = m2l_fma(D[24], m, L[3]);
     }
-    { const float m = __ldg(Ms + 22) * rp;
-      L[0] = fmaf(D[22], m, L[0]);
+    { const T m = -__ldg(Ms + 12) * rp;
+      L[0] = m2l_fma(D[12], m, L[0]);
+      L[1] = m2l_fma(D[22], m, L[1]);
+      L[2] = m2l_fma(D[24], m, L[2]);
+      L[3] = m2l_fma(D[25], m, L[3]);
     }
-    { const float m = __ldg(Ms + 23) * rp;
-      L[0] = fmaf(D[23], m, L[0]);
+    { const T m = -__ldg(Ms + 13) * rp;
+      L[0] = m2l_fma(D[13], m, L[0]);
+      L[1] = m2l_fma(D[23], m, L[1]);
+      L[2] = m2l_fma(D[26], m, L[2]);
+      L[3] = m2l_fma(D[27], m, L[3]);
     }
-    { const float m = __ldg(Ms + 24) * rp;
-      L[0] = fmaf(D[24], m, L[0]);
+    { const T m = -__ldg(Ms + 14) * rp;
+      L[0] = m2l_fma(D[14], m, L[0]);
+      L[1] = m2l_fma(D[24], m, L[1]);
+      L[2] = m2l_fma(D[27], m, L[2]);
+      L[3] = m2l_fma(D[28], m, L[3]);
     }
-    { const float m = __ldg(Ms + 25) * rp;
-      L[0] = fmaf(D[25], m, L[0]);
+    { const T m = -__ldg(Ms + 15) * rp;
+      L[0] = m2l_fma(D[15], m, L[0]);
+      L[1] = m2l_fma(D[25], m, L[1]);
+      L[2] = m2l_fma(D[28], m, L[2]);
+      L[3] = m2l_fma(D[29], m, L[3]);
     }
-    { const float m = __ldg(Ms + 26) * rp;
-      L[0] = fmaf(D[26], m, L[0]);
+    { const T m = -__ldg(Ms + 16) * rp;
+      L[0] = m2l_fma(D[16], m, L[0]);
+      L[1] = m2l_fma(D[26], m, L[1]);
+      L[2] = m2l_fma(D[30], m, L[2]);
+      L[3] = m2l_fma(D[31], m, L[3]);
     }
-    { const float m = __ldg(Ms + 27) * rp;
-      L[0] = fmaf(D[27], m, L[0]);
+    { const T m = -__ldg(Ms + 17) * rp;
+      L[0] = m2l_fma(D[17], m, L[0]);
+      L[1] = m2l_fma(D[27], m, L[1]);
+      L[2] = m2l_fma(D[31], m, L[2]);
+      L[3] = m2l_fma(D[32], m, L[3]);
     }
-    { const float m = __ldg(Ms + 28) * rp;
-      L[0] = fmaf(D[28], m, L[0]);
+    { const T m = -__ldg(Ms + 18) * rp;
+      L[0] = m2l_fma(D[18], m, L[0]);
+      L[1] = m2l_fma(D[28], m, L[1]);
+      L[2] = m2l_fma(D[32], m, L[2]);
+      L[3] = m2l_fma(D[33], m, L[3]);
     }
-    { const float m = __ldg(Ms + 29) * rp;
-      L[0] = fmaf(D[29], m, L[0]);
+    { const T m = -__ldg(Ms + 19) * rp;
+      L[0] = m2l_fma(D[19], m, L[0]);
+      L[1] = m2l_fma(D[29], m, L[1]);
+      L[2] = m2l_fma(D[33], m, L[2]);
+      L[3] = m2l_fma(D[34], m, L[3]);
     }
-    { const float m = __ldg(Ms + 30) * rp;
-      L[0] = fmaf(D[30], m, L[0]);
+    rp *= rho;
+    { const T m = __ldg(Ms + 20) * rp;
+      L[0] = m2l_fma(D[20], m, L[0]);
     }
-    { const float m = __ldg(Ms + 31) * rp;
-      L[0] = fmaf(D[31], m, L[0]);
+    { const T m = __ldg(Ms + 21) * rp;
+      L[0] = m2l_fma(D[21], m, L[0]);
     }
-    { const float m = __ldg(Ms + 32) * rp;
-      L[0] = fmaf(D[32], m, L[0]);
+    { const T m = __ldg(Ms + 22) * rp;
+      L[0] = m2l_fma(D[22], m, L[0]);
     }
-    { const float m = __ldg(Ms + 33) * rp;
-      L[0] = fmaf(D[33], m, L[0]);
+    { const T m = __ldg(Ms + 23) * rp;
+      L[0] = m2l_fma(D[23], m, L[0]);
     }
-    { const float m = __ldg(Ms + 34) * rp;
-      L[0] = fmaf(D[34], m, L[0]);
+    { const T m = __ldg(Ms + 24) * rp;
+      L[0] = m2l_fma(D[24], m, L[0]);
+    }
+    { const T m = __ldg(Ms + 25) * rp;
+      L[0] = m2l_fma(D[25], m, L[0]);
+    }
+    { const T m = __ldg(Ms + 26) * rp;
+      L[0] = m2l_fma(D[26], m, L[0]);
+    }
+    { const T m = __ldg(Ms + 27) * rp;
+      L[0] = m2l_fma(D[27], m, L[0]);
+    }
+    { const T m = __ldg(Ms + 28) * rp;
+      L[0] = m2l_fma(D[28], m, L[0]);
+    }
+    { const T m = __ldg(Ms + 29) * rp;
+      L[0] = m2l_fma(D[29], m, L[0]);
+    }
+    { const T m = __ldg(Ms + 30) * rp;
+      L[0] = m2l_fma(D[30], m, L[0]);
+    }
+    { const T m = __ldg(Ms + 31) * rp;
+      L[0] = m2l_fma(D[31], m, L[0]);
+    }
+    { const T m = __ldg(Ms + 32) * rp;
+      L[0] = m2l_fma(D[32], m, L[0]);
+    }
+    { const T m = __ldg(Ms + 33) * rp;
+      L[0] = m2l_fma(D[33], m, L[0]);
+    }
+    { const T m = __ldg(Ms + 34) * rp;
+      L[0] = m2l_fma(D[34], m, L[0]);
     }
 }
 
-__device__ __forceinline__ void m2l_side_b_4(const float (&D)[35], const float *__restrict__ Ms, float (&L)[35])
+template <class T> __device__ __forceinline__ void m2l_side_b_4(const T (&D)[35], const T *__restrict__ Ms, T (&L)[35])
 {
-    { const float m = __ldg(Ms + 0);
+    { const T m = __ldg(Ms + 0);
       L[0] = D[0] * m;
       L[1] = -D[1] * m;
       L[2] = -D[2] * m;
@@ -1242,256 +1249,256 @@ __device__ __forceinline__ void m2l_side_b_4(const float (&D)[35], const float *
       L[33] = D[33] * m;
       L[34] = D[34] * m;
     }
-    { const float m = __ldg(Ms + 1);
-      L[0] = fmaf(D[1], m, L[0]);
-      L[1] = fmaf(-D[4], m, L[1]);
-      L[2] = fmaf(-D[5], m, L[2]);
-      L[3] = fmaf(-D[6], m, L[3]);
-      L[4] = fmaf(D[10], m, L[4]);
-      L[5] = fmaf(D[11], m, L[5]);
-      L[6] = fmaf(D[12], m, L[6]);
-      L[7] = fmaf(D[13], m, L[7]);
-      L[8] = fmaf(D[14], m, L[8]);
-      L[9] = fmaf(D[15], m, L[9]);
-      L[10] = fmaf(-D[20], m, L[10]);
-      L[11] = fmaf(-D[21], m, L[11]);
-      L[12] = fmaf(-D[22], m, L[12]);
-      L[13] = fmaf(-D[23], m, L[13]);
-      L[14] = fmaf(-D[24], m, L[14]);
-      L[15] = fmaf(-D[25], m, L[15]);
-      L[16] = fmaf(-D[26], m, L[16]);
-      L[17] = fmaf(-D[27], m, L[17]);
-      L[18] = fmaf(-D[28], m, L[18]);
-      L[19] = fmaf(-D[29], m, L[19]);
+    { const T m = __ldg(Ms + 1);
+      L[0] = m2l_fma(D[1], m, L[0]);
+      L[1] = m2l_fma(-D[4], m, L[1]);
+      L[2] = m2l_fma(-D[5], m, L[2]);
+      L[3] = m2l_fma(-D[6], m, L[3]);
+      L[4] = m2l_fma(D[10], m, L[4]);
+      L[5] = m2l_fma(D[11], m, L[5]);
+      L[6] = m2l_fma(D[12], m, L[6]);
+      L[7] = m2l_fma(D[13], m, L[7]);
+      L[8] = m2l_fma(D[14], m, L[8]);
+      L[9] = m2l_fma(D[15], m, L[9]);
+      L[10] = m2l_fma(-D[20], m, L[10]);
+      L[11] = m2l_fma(-D[21], m, L[11]);
+      L[12] = m2l_fma(-D[22], m, L[12]);
+      L[13] = m2l_fma(-D[23], m, L[13]);
+      L[14] = m2l_fma(-D[24], m, L[14]);
+      L[15] = m2l_fma(-D[25], m, L[15]);
+      L[16] = m2l_fma(-D[26], m, L[16]);
+      L[17] = m2l_fma(-D[27], m, L[17]);
+      L[18] = m2l_fma(-D[28], m, L[18]);
+      L[19] = m2l_fma(-D[29], m, L[19]);
     }
-    { const float m = __ldg(Ms + 2);
-      L[0] = fmaf(D[2], m, L[0]);
-      L[1] = fmaf(-D[5], m, L[1]);
-      L[2] = fmaf(-D[7], m, L[2]);
-      L[3] = fmaf(-D[8], m, L[3]);
-      L[4] = fmaf(D[11], m, L[4]);
-      L[5] = fmaf(D[13], m, L[5]);
-      L[6] = fmaf(D[14], m, L[6]);
-      L[7] = fmaf(D[16], m, L[7]);
-      L[8] = fmaf(D[17], m, L[8]);
-      L[9] = fmaf(D[18], m, L[9]);
-      L[10] = fmaf(-D[21], m, L[10]);
-      L[11] = fmaf(-D[23], m, L[11]);
-      L[12] = fmaf(-D[24], m, L[12]);
-      L[13] = fmaf(-D[26], m, L[13]);
-      L[14] = fmaf(-D[27], m, L[14]);
-      L[15] = fmaf(-D[28], m, L[15]);
-      L[16] = fmaf(-D[30], m, L[16]);
-      L[17] = fmaf(-D[31], m, L[17]);
-      L[18] = fmaf(-D[32], m, L[18]);
-      L[19] = fmaf(-D[33], m, L[19]);
+    { const T m = __ldg(Ms + 2);
+      L[0] = m2l_fma(D[2], m, L[0]);
+      L[1] = m2l_fma(-D[5], m, L[1]);
+      L[2] = m2l_fma(-D[7], m, L[2]);
+      L[3] = m2l_fma(-D[8], m, L[3]);
+      L[4] = m2l_fma(D[11], m, L[4]);
+      L[5] = m2l_fma(D[13], m, L[5]);
+      L[6] = m2l_fma(D[14], m, L[6]);
+      L[7] = m2l_fma(D[16], m, L[7]);
+      L[8] = m2l_fma(D[17], m, L[8]);
+      L[9] = m2l_fma(D[18], m, L[9]);
+      L[10] = m2l_fma(-D[21], m, L[10]);
+      L[11] = m2l_fma(-D[23], m, L[11]);
+      L[12] = m2l_fma(-D[24], m, L[12]);
+      L[13] = m2l_fma(-D[26], m, L[13]);
+      L[14] = m2l_fma(-D[27], m, L[14]);
+      L[15] = m2l_fma(-D[28], m, L[15]);
+      L[16] = m2l_fma(-D[30], m, L[16]);
+      L[17] = m2l_fma(-D[31], m, L[17]);
+      L[18] = m2l_fma(-D[32], m, L[18]);
+      L[19] = m2l_fma(-D[33], m, L[19]);
     }
-    { const float m = __ldg(Ms + 3);
-      L[0] = fmaf(D[3], m, L[0]);
-      L[1] = fmaf(-D[6], m, L[1]);
-      L[2] = fmaf(-D[8], m, L[2]);
-      L[3] = fmaf(-D[9], m, L[3]);
-      L[4] = fmaf(D[12], m, L[4]);
-      L[5] = fmaf(D[14], m, L[5]);
-      L[6] = fmaf(D[15], m, L[6]);
-      L[7] = fmaf(D[17], m, L[7]);
-      L[8] = fmaf(D[18], m, L[8]);
-      L[9] = fmaf(D[19], m, L[9]);
-      L[10] = fmaf(-D[22], m, L[10]);
-      L[11] = fmaf(-D[24], m, L[11]);
-      L[12] = fmaf(-D[25], m, L[12]);
-      L[13] = fmaf(-D[27], m, L[13]);
-      L[14] = fmaf(-D[28], m, L[14]);
-      L[15] = fmaf(-D[29], m, L[15]);
-      L[16] = fmaf(-D[31], m, L[16]);
-      L[17] = fmaf(-D[32], m, L[17]);
-      L[18] = fmaf(-D[33], m, L[18]);
-      L[19] = fmaf(-D[34], m, L[19]);
+    { const T m = __ldg(Ms + 3);
+      L[0] = m2l_fma(D[3], m, L[0]);
+      L[1] = m2l_fma(-D[6], m, L[1]);
+      L[2] = m2l_fma(-D[8], m, L[2]);
+      L[3] = m2l_fma(-D[9], m, L[3]);
+      L[4] = m2l_fma(D[12], m, L[4]);
+      L[5] = m2l_fma(D[14], m, L[5]);
+      L[6] = m2l_fma(D[15], m, L[6]);
+      L[7] = m2l_fma(D[17], m, L[7]);
+      L[8] = m2l_fma(D[18], m, L[8]);
+      L[9] = m2l_fma(D[19], m, L[9]);
+      L[10] = m2l_fma(-D[22], m, L[10]);
+      L[11] = m2l_fma(-D[24], m, L[11]);
+      L[12] = m2l_fma(-D[25], m, L[12]);
+      L[13] = m2l_fma(-D[27], m, L[13]);
+      L[14] = m2l_fma(-D[28], m, L[14]);
+      L[15] = m2l_fma(-D[29], m, L[15]);
+      L[16] = m2l_fma(-D[31], m, L[16]);
+      L[17] = m2l_fma(-D[32], m, L[17]);
+      L[18] = m2l_fma(-D[33], m, L[18]);
+      L[19] = m2l_fma(-D[34], m, L[19]);
     }
-    { const float m = __ldg(Ms + 4);
-      L[0] = fmaf(D[4], m, L[0]);
-      L[1] = fmaf(-D[10], m, L[1]);
-      L[2] = fmaf(-D[11], m, L[2]);
-      L[3] = fmaf(-D[12], m, L[3]);
-      L[4] = fmaf(D[20], m, L[4]);
-      L[5] = fmaf(D[21], m, L[5]);
-      L[6] = fmaf(D[22], m, L[6]);
-      L[7] = fmaf(D[23], m, L[7]);
-      L[8] = fmaf(D[24], m, L[8]);
-      L[9] = fmaf(D[25], m, L[9]);
+    { const T m = __ldg(Ms + 4);
+      L[0] = m2l_fma(D[4], m, L[0]);
+      L[1] = m2l_fma(-D[10], m, L[1]);
+      L[2] = m2l_fma(-D[11], m, L[2]);
+      L[3] = m2l_fma(-D[12], m, L[3]);
+      L[4] = m2l_fma(D[20], m, L[4]);
+      L[5] = m2l_fma(D[21], m, L[5]);
+      L[6] = m2l_fma(D[22], m, L[6]);
+      L[7] = m2l_fma(D[23], m, L[7]);
+      L[8] = m2l_fma(D[24], m, L[8]);
+      L[9] = m2l_fma(D[25], m, L[9]);
     }
-    { const float m = __ldg(Ms + 5);
-      L[0] = fmaf(D[5], m, L[0]);
-      L[1] = fmaf(-D[11], m, L[1]);
-      L[2] = fmaf(-D[13], m, L[2]);
-      L[3] = fmaf(-D[14], m, L[3]);
-      L[4] = fmaf(D[21], m, L[4]);
-      L[5] = fmaf(D[23], m, L[5]);
-      L[6] = fmaf(D[24], m, L[6]);
-      L[7] = fmaf(D[26], m, L[7]);
-      L[8] = fmaf(D[27], m, L[8]);
-      L[9] = fmaf(D[28], m, L[9]);
+    { const T m = __ldg(Ms + 5);
+      L[0] = m2l_fma(D[5], m, L[0]);
+      L[1] = m2l_fma(-D[11], m, L[1]);
+      L[2] = m2l_fma(-D[13], m, L[2]);
+      L[3] = m2l_fma(-D[14], m, L[3]);
+      L[4] = m2l_fma(D[21], m, L[4]);
+      L[5] = m2l_fma(D[23], m, L[5]);
+      L[6] = m2l_fma(D[24], m, L[6]);
+      L[7] = m2l_fma(D[26], m, L[7]);
+      L[8] = m2l_fma(D[27], m, L[8]);
+      L[9] = m2l_fma(D[28], m, L[9]);
     }
-    { const float m = __ldg(Ms + 6);
-      L[0] = fmaf(D[6], m, L[0]);
-      L[1] = fmaf(-D[12], m, L[1]);
-      L[2] = fmaf(-D[14], m, L[2]);
-      L[3] = fmaf(-D[15], m, L[3]);
-      L[4] = fmaf(D[22], m, L[4]);
-      L[5] = fmaf(D[24], m, L[5]);
-      L[6] = fmaf(D[25], m, L[6]);
-      L[7] = fmaf(D[27], m, L[7]);
-      L[8] = fmaf(D[28], m, L[8]);
-      L[9] = fmaf(D[29], m, L[9]);
+    { const T m = __ldg(Ms + 6);
+      L[0] = m2l_fma(D[6], m, L[0]);
+      L[1] = m2l_fma(-D[12], m, L[1]);
+      L[2] = m2l_fma(-D[14], m, L[2]);
+      L[3] = m2l_fma(-D[15], m, L[3]);
+      L[4] = m2l_fma(D[22], m, L[4]);
+      L[5] = m2l_fma(D[24], m, L[5]);
+      L[6] = m2l_fma(D[25], m, L[6]);
+      L[7] = m2l_fma(D[27], m, L[7]);
+      L[8] = m2l_fma(D[28], m, L[8]);
+      L[9] = m2l_fma(D[29], m, L[9]);
     }
-    { const float m = __ldg(Ms + 7);
-      L[0] = fmaf(D[7], m, L[0]);
-      L[1] = fmaf(-D[13], m, L[1]);
-      L[2] = fmaf(-D[16], m, L[2]);
-      L[3] = fmaf(-D[17], m, L[3]);
-      L[4] = fmaf(D[23], m, L[4]);
-      L[5] = fmaf(D[26], m, L[5]);
-      L[6] = fmaf(D[27], m, L[6]);
-      L[7] = fmaf(D[30], m, L[7]);
-      L[8] = fmaf(D[31], m, L[8]);
-      L[9] = fmaf(D[32], m, L[9]);
+    { const T m = __ldg(Ms + 7);
+      L[0] = m2l_fma(D[7], m, L[0]);
+      L[1] = m2l_fma(-D[13], m, L[1]);
+      L[2] = m2l_fma(-D[16], m, L[2]);
+      L[3] = m2l_fma(-D[17], m, L[3]);
+      L[4] = m2l_fma(D[23], m, L[4]);
+      L[5] = m2l_fma(D[26], m, L[5]);
+      L[6] = m2l_fma(D[27], m, L[6]);
+      L[7] = m2l_fma(D[30], m, L[7]);
+      L[8] = m2l_fma(D[31], m, L[8]);
+      L[9] = m2l_fma(D[32], m, L[9]);
     }
-    { const float m = __ldg(Ms + 8);
-      L[0] = fmaf(D[8], m, L[0]);
-      L[1] = fmaf(-D[14], m, L[1]);
-      L[2] = fmaf(-D[17], m, L[2]);
-      L[3] = fmaf(-D[18], m, L[3]);
-      L[4] = fmaf(D[24], m, L[4]);
-      L[5] = fmaf(D[27], m, L[5]);
-      L[6] = fmaf(D[28], m, L[6]);
-      L[7] = fmaf(D[31], m, L[7]);
-      L[8] = fmaf(D[32], m, L[8]);
-      L[9] = fmaf(D[33], m, L[9]);
+    { const T m = __ldg(Ms + 8);
+      L[0] = m2l_fma(D[8], m, L[0]);
+      L[1] = m2l_fma(-D[14], m, L[1]);
+      L[2] = m2l_fma(-D[17], m, L[2]);
+      L[3] = m2l_fma(-D[18], m, L[3]);
+      L[4] = m2l_fma(D[24], m, L[4]);
+      L[5] = m2l_fma(D[27], m, L[5]);
+      L[6] = m2l_fma(D[28], m, L[6]);
+      L[7] = m2l_fma(D[31], m, L[7]);
+      L[8] = m2l_fma(D[32], m, L[8]);
+      L[9] = m2l_fma(D[33], m, L[9]);
     }
-    { const float m = __ldg(Ms + 9);
-      L[0] = fmaf(D[9], m, L[0]);
-      L[1] = fmaf(-D[15], m, L[1]);
-      L[2] = fmaf(-D[18], m, L[2]);
-      L[3] = fmaf(-D[19], m, L[3]);
-      L[4] = fmaf(D[25], m, L[4]);
-      L[5] = fmaf(D[28], m, L[5]);
-      L[6] = fmaf(D[29], m, L[6]);
-      L[7] = fmaf(D[32], m, L[7]);
-      L[8] = fmaf(D[33], m, L[8]);
-      L[9] = fmaf(D[34], m, L[9]);
+    { const T m = __ldg(Ms + 9);
+      L[0] = m2l_fma(D[9], m, L[0]);
+      L[1] = m2l_fma(-D[15], m, L[1]);
+      L[2] = m2l_fma(-D[18], m, L[2]);
+      L[3] = m2l_fma(-D[19], m, L[3]);
+      L[4] = m2l_fma(D[25], m, L[4]);
+      L[5] = m2l_fma(D[28], m, L[5]);
+      L[6] = m2l_fma(D[29], m, L[6]);
+      L[7] = m2l_fma(D[32], m, L[7]);
+      L[8] = m2l_fma(D[33], m, L[8]);
+      L[9] = m2l_fma(D[34], m, L[9]);
     }
-    { const float m = __ldg(Ms + 10);
-      L[0] = fmaf(D[10], m, L[0]);
-      L[1] = fmaf(-D[20], m, L[1]);
-      L[2] = fmaf(-D[21], m, L[2]);
-      L[3] = fmaf(-D[22], m, L[3]);
+    { const T m = __ldg(Ms + 10);
+      L[0] = m2l_fma(D[10], m, L[0]);
+      L[1] = m2l_fma(-D[20], m, L[1]);
+      L[2] = m2l_fma(-D[21], m, L[2]);
+      L[3] = m2l_fma(-D[22], m, L[3]);
     }
-    { const float m = __ldg(Ms + 11);
-      L[0] = fmaf(D[11], m, L[0]);
-      L[1] = fmaf(-D[21], m, L[1]);
-      L[2] = fmaf(-D[23], m, L[2]);
-      L[3] = fmaf(-D[24], m, L[3]);
+    { const T m = __ldg(Ms + 11);
+      L[0] = m2l_fma(D[11], m, L[0]);
+      L[1] = m2l_fma(-D[21], m, L[1]);
+      L[2] = m2l_fma(-D[23], m, L[2]);
+      L[3] = m2l_fma(-D[24], m, L[3]);
     }
-    { const float m = __ldg(Ms + 12);
-      L[0] = fmaf(D[12], m, L[0]);
-      L[1] = fmaf(-D[22], m, L[1]);
-      L[2] = fmaf(-D[24], m, L[2]);
-      L[3] = fmaf(-D[25], m, L[3]);
+    { const T m = __ldg(Ms + 12);
+      L[0] = m2l_fma(D[12], m, L[0]);
+      L[1] = m2l_fma(-D[22], m, L[1]);
+      L[2] = m2l_fma(-D[24], m, L[2]);
+      L[3] = m2l_fma(-D[25], m, L[3]);
     }
-    { const float m = __ldg(Ms + 13);
-      L[0] = fmaf(D[13], m, L[0]);
-      L[1] = fmaf(-D[23], m, L[1]);
-      L[2] = fmaf(-D[26], m, L[2]);
-      L[3] = fmaf(-D[27], m, L[3]);
+    { const T m = __ldg(Ms + 13);
+      L[0] = m2l_fma(D[13], m, L[0]);
+      L[1] = m2l_fma(-D[23], m, L[1]);
+      L[2] = m2l_fma(-D[26], m, L[2]);
+      L[3] = m2l_fma(-D[27], m, L[3]);
     }
-    { const float m = __ldg(Ms + 14);
-      L[0] = fmaf(D[14], m, L[0]);
-      L[1] = fmaf(-D[24], m, L[1]);
-      L[2] = fmaf(-D[27], m, L[2]);
-      L[3] = fmaf(-D[28], m, L[3]);
+    { const T m = __ldg(Ms + 14);
+      L[0] = m2l_fma(D[14], m, L[0]);
+      L[1] = m2l_fma(-D[24], m, L[1]);
+      L[2] = m2l_fma(-D[27], m, L[2]);
+      L[3] = m2l_fma(-D[28], m, L[3]);
     }
-    { const float m = __ldg(Ms + 15);
-      L[0] = fmaf(D[15], m, L[0]);
-      L[1] = fmaf(-D[25], m, L[1]);
-      L[2] = fmaf(-D[28], m, L[2]);
-      L[3] = fmaf(-D[29], m, L[3]);
+    { const T m = __ldg(Ms + 15);
+      L[0] = m2l_fma(D[15], m, L[0]);
+      L[1] = m2l_fma(-D[25], m, L[1]);
+      L[2] = m2l_fma(-D[28], m, L[2]);
+      L[3] = m2l_fma(-D[29], m, L[3]);
     }
-    { const float m = __ldg(Ms + 16);
-      L[0] = fmaf(D[16], m, L[0]);
-      L[1] = fmaf(-D[26], m, L[1]);
-      L[2] = fmaf(-D[30], m, L[2]);
-      L[3] = fmaf(-D[31], m, L[3]);
+    { const T m = __ldg(Ms + 16);
+      L[0] = m2l_fma(D[16], m, L[0]);
+      L[1] = m2l_fma(-D[26], m, L[1]);
+      L[2] = m2l_fma(-D[30], m, L[2]);
+      L[3] = m2l_fma(-D[31], m, L[3]);
     }
-    { const float m = __ldg(Ms + 17);
-      L[0] = fmaf(D[17], m, L[0]);
-      L[1] = fmaf(-D[27], m, L[1]);
-      L[2] = fmaf(-D[31], m, L[2]);
-      L[3] = fmaf(-D[32], m, L[3]);
+    { const T m = __ldg(Ms + 17);
+      L[0] = m2l_fma(D[17], m, L[0]);
+      L[1] = m2l_fma(-D[27], m, L[1]);
+      L[2] = m2l_fma(-D[31], m, L[2]);
+      L[3] = m2l_fma(-D[32], m, L[3]);
     }
-    { const float m = __ldg(Ms + 18);
-      L[0] = fmaf(D[18], m, L[0]);
-      L[1] = fmaf(-D[28], m, L[1]);
-      L[2] = fmaf(-D[32], m, L[2]);
-      L[3] = fmaf(-D[33], m, L[3]);
+    { const T m = __ldg(Ms + 18);
+      L[0] = m2l_fma(D[18], m, L[0]);
+      L[1] = m2l_fma(-D[28], m, L[1]);
+      L[2] = m2l_fma(-D[32], m, L[2]);
+      L[3] = m2l_fma(-D[33], m, L[3]);
     }
-    { const float m = __ldg(Ms + 19);
-      L[0] = fmaf(D[19], m, L[0]);
-      L[1] = fmaf(-D[29], m, L[1]);
-      L[2] = fmaf(-D[33], m, L[2]);
-      L[3] = fmaf(-D[34], m, L[3]);
+    { const T m = __ldg(Ms + 19);
+      L[0] = m2l_fma(D[19], m, L[0]);
+      L[1] = m2l_fma(-D[29], m, L[1]);
+      L[2] = m2l_fma(-D[33], m, L[2]);
+      L[3] = m2l_fma(-D[34], m, L[3]);
     }
-    { const float m = __ldg(Ms + 20);
-      L[0] = fmaf(D[20], m, L[0]);
+    { const T m = __ldg(Ms + 20);
+      L[0] = m2l_fma(D[20], m, L[0]);
     }
-    { const float m = __ldg(Ms + 21);
-      L[0] = fmaf(D[21], m, L[0]);
+    { const T m = __ldg(Ms + 21);
+      L[0] = m2l_fma(D[21], m, L[0]);
     }
-    { const float m = __ldg(Ms + 22);
-      L[0] = fmaf(D[22], m, L[0]);
+    { const T m = __ldg(Ms + 22);
+      L[0] = m2l_fma(D[22], m, L[0]);
     }
-    { const float m = __ldg(Ms + 23);
-      L[0] = fmaf(D[23], m, L[0]);
+    { const T m = __ldg(Ms + 23);
+      L[0] = m2l_fma(D[23], m, L[0]);
     }
-    { const float m = __ldg(Ms + 24);
-      L[0] = fmaf(D[24], m, L[0]);
+    { const T m = __ldg(Ms + 24);
+      L[0] = m2l_fma(D[24], m, L[0]);
     }
-    { const float m = __ldg(Ms + 25);
-      L[0] = fmaf(D[25], m, L[0]);
+    { const T m = __ldg(Ms + 25);
+      L[0] = m2l_fma(D[25], m, L[0]);
     }
-    { const float m = __ldg(Ms + 26);
-      L[0] = fmaf(D[26], m, L[0]);
+    { const T m = __ldg(Ms + 26);
+      L[0] = m2l_fma(D[26], m, L[0]);
     }
-    { const float m = __ldg(Ms + 27);
-      L[0] = fmaf(D[27], m, L[0]);
+    { const T m = __ldg(Ms + 27);
+      L[0] = m2l_fma(D[27], m, L[0]);
     }
-    { const float m = __ldg(Ms + 28);
-      L[0] = fmaf(D[28], m, L[0]);
+    { const T m = __ldg(Ms + 28);
+      L[0] = m2l_fma(D[28], m, L[0]);
     }
-    { const float m = __ldg(Ms + 29);
-      L[0] = fmaf(D[29], m, L[0]);
+    { const T m = __ldg(Ms + 29);
+      L[0] = m2l_fma(D[29], m, L[0]);
     }
-    { const float m = __ldg(Ms + 30);
-      L[0] = fmaf(D[30], m, L[0]);
+    { const T m = __ldg(Ms + 30);
+      L[0] = m2l_fma(D[30], m, L[0]);
     }
-    { const float m = __ldg(Ms + 31);
-      L[0] = fmaf(D[31], m, L[0]);
+    { const T m = __ldg(Ms + 31);
+      L[0] = m2l_fma(D[31], m, L[0]);
     }
-    { const float m = __ldg(Ms + 32);
-      L[0] = fmaf(D[32], m, L[0]);
+    { const T m = __ldg(Ms + 32);
+      L[0] = m2l_fma(D[32], m, L[0]);
     }
-    { const float m = __ldg(Ms + 33);
-      L[0] = fmaf(D[33], m, L[0]);
+    { const T m = __ldg(Ms + 33);
+      L[0] = m2l_fma(D[33], m, L[0]);
     }
-    { const float m = __ldg(Ms + 34);
-      L[0] = fmaf(D[34], m, L[0]);
+    { const T m = __ldg(Ms + 34);
+      L[0] = m2l_fma(D[34], m, L[0]);
     }
 }
 
-__device__ __forceinline__ void m2l_side_a_forces_4(const float (&D)[35], const float *__restrict__ Ms, float rho, float (&L)[35])
+template <class T> __device__ __forceinline__ void m2l_side_a_forces_4(const T (&D)[35], const T *__restrict__ Ms, T rho, T (&L)[35])
 {
-    L[0] = 0.0f;
-    float rp = 1.0f;
-    { const float m = __ldg(Ms + 0) * rp;
+    L[0] = T(0);
+    T rp = T(1);
+    { const T m = __ldg(Ms + 0) * rp;
       L[1] = D[1] * m;
       L[2] = D[2] * m;
       L[3] = D[3] * m;
@@ -1528,193 +1535,193 @@ __device__ __forceinline__ void m2l_side_a_forces_4(const float (&D)[35], const 
       L[34] = D[34] * m;
     }
     rp *= rho;
-    { const float m = -__ldg(Ms + 1) * rp;
-      L[1] = fmaf(D[4], m, L[1]);
-      L[2] = fmaf(D[5], m, L[2]);
-      L[3] = fmaf(D[6], m, L[3]);
-      L[4] = fmaf(D[10], m, L[4]);
-      L[5] = fmaf(D[11], m, L[5]);
-      L[6] = fmaf(D[12], m, L[6]);
-      L[7] = fmaf(D[13], m, L[7]);
-      L[8] = fmaf(D[14], m, L[8]);
-      L[9] = fmaf(D[15], m, L[9]);
-      L[10] = fmaf(D[20], m, L[10]);
-      L[11] = fmaf(D[21], m, L[11]);
-      L[12] = fmaf(D[22], m, L[12]);
-      L[13] = fmaf(D[23], m, L[13]);
-      L[14] = fmaf(D[24], m, L[14]);
-      L[15] = fmaf(D[25], m, L[15]);
-      L[16] = fmaf(D[26], m, L[16]);
-      L[17] = fmaf(D[27], m, L[17]);
-      L[18] = fmaf(D[28], m, L[18]);
-      L[19] = fmaf(D[29], m, L[19]);
+    { const T m = -__ldg(Ms + 1) * rp;
+      L[1] = m2l_fma(D[4], m, L[1]);
+      L[2] = m2l_fma(D[5], m, L[2]);
+      L[3] = m2l_fma(D[6], m, L[3]);
+      L[4] = m2l_fma(D[10], m, L[4]);
+      L[5] = m2l_fma(D[11], m, L[5]);
+      L[6] = m2l_fma(D[12], m, L[6]);
+      L[7] = m2l_fma(D[13], m, L[7]);
+      L[8] = m2l_fma(D[14], m, L[8]);
+      L[9] = m2l_fma(D[15], m, L[9]);
+      L[10] = m2l_fma(D[20], m, L[10]);
+      L[11] = m2l_fma(D[21], m, L[11]);
+      L[12] = m2l_fma(D[22], m, L[12]);
+      L[13] = m2l_fma(D[23], m, L[13]);
+      L[14] = m2l_fma(D[24], m, L[14]);
+      L[15] = m2l_fma(D[25], m, L[15]);
+      L[16] = m2l_fma(D[26], m, L[16]);
+      L[17] = m2l_fma(D[27], m, L[17]);
+      L[18] = m2l_fma(D[28], m, L[18]);
+      L[19] = m2l_fma(D[29], m, L[19]);
     }
-    { const float m = -__ldg(Ms + 2) * rp;
-      L[1] = fmaf(D[5], m, L[1]);
-      L[2] = fmaf(D[7], m, L[2]);
-      L[3] = fmaf(D[8], m, L[3]);
-      L[4] = fmaf(D[11], m, L[4]);
-      L[5] = fmaf(D[13], m, L[5]);
-      L[6] = fmaf(D[14], m, L[6]);
-      L[7] = fmaf(D[16], m, L[7]);
-      L[8] = fmaf(D[17], m, L[8]);
-      L[9] = fmaf(D[18], m, L[9]);
-      L[10] = fmaf(D[21], m, L[10]);
-      L[11] = fmaf(D[23], m, L[11]);
-      L[12] = fmaf(D[24], m, L[12]);
-      L[13] = fmaf(D[26], m, L[13]);
-      L[14] = fmaf(D[27], m, L[14]);
-      L[15] = fmaf(D[28], m, L[15]);
-      L[16] = fmaf(D[30], m, L[16]);
-      L[17] = fmaf(D[31], m, L[17]);
-      L[18] = fmaf(D[32], m, L[18]);
-      L[19] = fmaf(D[33], m, L[19]);
+    { const T m = -__ldg(Ms + 2) * rp;
+      L[1] = m2l_fma(D[5], m, L[1]);
+      L[2] = m2l_fma(D[7], m, L[2]);
+      L[3] = m2l_fma(D[8], m, L[3]);
+      L[4] = m2l_fma(D[11], m, L[4]);
+      L[5] = m2l_fma(D[13], m, L[5]);
+      L[6] = m2l_fma(D[14], m, L[6]);
+      L[7] = m2l_fma(D[16], m, L[7]);
+      L[8] = m2l_fma(D[17], m, L[8]);
+      L[9] = m2l_fma(D[18], m, L[9]);
+      L[10] = m2l_fma(D[21], m, L[10]);
+      L[11] = m2l_fma(D[23], m, L[11]);
+      L[12] = m2l_fma(D[24], m, L[12]);
+      L[13] = m2l_fma(D[26], m, L[13]);
+      L[14] = m2l_fma(D[27], m, L[14]);
+      L[15] = m2l_fma(D[28], m, L[15]);
+      L[16] = m2l_fma(D[30], m, L[16]);
+      L[17] = m2l_fma(D[31], m, L[17]);
+      L[18] = m2l_fma(D[32], m, L[18]);
+      L[19] = m2l_fma(D[33], m, L[19]);
     }
-    { const float m = -__ldg(Ms + 3) * rp;
-      L[1] = fmaf(D[6], m, L[1]);
-      L[2] = fmaf(D[8], m, L[2]);
-      L[3] = fmaf(D[9], m, L[3]);
-      L[4] = fmaf(D[12], m, L[4]);
-      L[5] = fmaf(D[14], m, L[5]);
-      L[6] = fmaf(D[15], m, L[6]);
-      L[7] = fmaf(D[17], m, L[7]);
-      L[8] = fmaf(D[18], m, L[8]);
-      L[9] = fmaf(D[19], m, L[9]);
-      L[10] = fmaf(D[22], m, L[10]);
-      L[11] = fmaf(D[24], m, L[11]);
-      L[12] = fmaf(D[25], m, L[12]);
-      L[13] = fmaf(D[27], m, L[13]);
-      L[14] = fmaf(D[28], m, L[14]);
-      L[15] = fmaf(D[29], m, L[15]);
-      L[16] = fmaf(D[31], m, L[16]);
-      L[17] = fmaf(D[32], m, L[17]);
-      L[18] = fmaf(D[33], m, L[18]);
-      L[19] = fmaf(D[34], m, L[19]);
-    }
-    rp *= rho;
-    { const float m = __ldg(Ms + 4) * rp;
-      L[1] = fmaf(D[10], m, L[1]);
-      L[2] = fmaf(D[11], m, L[2]);
-      L[3] = fmaf(D[12], m, L[3]);
-      L[4] = fmaf(D[20], m, L[4]);
-      L[5] = fmaf(D[21], m, L[5]);
-      L[6] = fmaf(D[22], m, L[6]);
-      L[7] = fmaf(D[23], m, L[7]);
-      L[8] = fmaf(D[24], m, L[8]);
-      L[9] = fmaf(D[25], m, L[9]);
-    }
-    { const float m = __ldg(Ms + 5) * rp;
-      L[1] = fmaf(D[11], m, L[1]);
-      L[2] = fmaf(D[13], m, L[2]);
-      L[3] = fmaf(D[14], m, L[3]);
-      L[4] = fmaf(D[21], m, L[4]);
-      L[5] = fmaf(D[23], m, L[5]);
-      L[6] = fmaf(D[24], m, L[6]);
-      L[7] = fmaf(D[26], m, L[7]);
-      L[8] = fmaf(D[27], m, L[8]);
-      L[9] = fmaf(D[28], m, L[9]);
-    }
-    { const float m = __ldg(Ms + 6) * rp;
-      L[1] = fmaf(D[12], m, L[1]);
-      L[2] = fmaf(D[14], m, L[2]);
-      L[3] = fmaf(D[15], m, L[3]);
-      L[4] = fmaf(D[22], m, L[4]);
-      L[5] = fmaf(D[24], m, L[5]);
-      L[6] = fmaf(D[25], m, L[6]);
-      L[7] = fmaf(D[27], m, L[7]);
-      L[8] = fmaf(D[28], m, L[8]);
-      L[9] = fmaf(D[29], m, L[9]);
-    }
-    { const float m = __ldg(Ms + 7) * rp;
-      L[1] = fmaf(D[13], m, L[1]);
-      L[2] = fmaf(D[16], m, L[2]);
-      L[3] = fmaf(D[17], m, L[3]);
-      L[4] = fmaf(D[23], m, L[4]);
-      L[5] = fmaf(D[26], m, L[5]);
-      L[6] = fmaf(D[27], m, L[6]);
-      L[7] = fmaf(D[30], m, L[7]);
-      L[8] = fmaf(D[31], m, L[8]);
-      L[9] = fmaf(D[32], m, L[9]);
-    }
-    { const float m = __ldg(Ms + 8) * rp;
-      L[1] = fmaf(D[14], m, L[1]);
-      L[2] = fmaf(D[17], m, L[2]);
-      L[3] = fmaf(D[18], m, L[3]);
-      L[4] = fmaf(D[24], m, L[4]);
-      L[5] = fmaf(D[27], m, L[5]);
-      L[6] = fmaf(D[28], m, L[6]);
-      L[7] = fmaf(D[31], m, L[7]);
-      L[8] = fmaf(D[32], m, L[8]);
-      L[9] = fmaf(D[33], m, L[9]);
-    }
-    { const float m = __ldg(Ms + 9) * rp;
-      L[1] = fmaf(D[15], m, L[1]);
-      L[2] = fmaf(D[18], m, L[2]);
-      L[3] = fmaf(D[19], m, L[3]);
-      L[4] = fmaf(D[25], m, L[4]);
-      L[5] = fmaf(D[28], m, L[5]);
-      L[6] = fmaf(D[29], m, L[6]);
-      L[7] = fmaf(D[32], m, L[7]);
-      L[8] = fmaf(D[33], m, L[8]);
-      L[9] = fmaf(D[34], m, L[9]);
+    { const T m = -__ldg(Ms + 3) * rp;
+      L[1] = m2l_fma(D[6], m, L[1]);
+      L[2] = m2l_fma(D[8], m, L[2]);
+      L[3] = m2l_fma(D[9], m, L[3]);
+      L[4] = m2l_fma(D[12], m, L[4]);
+      L[5] = m2l_fma(D[14], m, L[5]);
+      L[6] = m2l_fma(D[15], m, L[6]);
+      L[7] = m2l_fma(D[17], m, L[7]);
+      L[8] = m2l_fma(D[18], m, L[8]);
+      L[9] = m2l_fma(D[19], m, L[9]);
+      L[10] = m2l_fma(D[22], m, L[10]);
+      L[11] = m2l_fma(D[24], m, L[11]);
+      L[12] = m2l_fma(D[25], m, L[12]);
+      L[13] = m2l_fma(D[27], m, L[13]);
+      L[14] = m2l_fma(D[28], m, L[14]);
+      L[15] = m2l_fma(D[29], m, L[15]);
+      L[16] = m2l_fma(D[31], m, L[16]);
+      L[17] = m2l_fma(D[32], m, L[17]);
+      L[18] = m2l_fma(D[33], m, L[18]);
+      L[19] = m2l_fma(D[34], m, L[19]);
     }
     rp *= rho;
-    { const float m = -__ldg(Ms + 10) * rp;
-      L[1] = fmaf(D[20], m, L[1]);
-      L[2] = fmaf(D[21], m, L[2]);
-      L[3] = fmaf(D[22], m, L[3]);
+    { const T m = __ldg(Ms + 4) * rp;
+      L[1] = m2l_fma(D[10], m, L[1]);
+      L[2] = m2l_fma(D[11], m, L[2]);
+      L[3] = m2l_fma(D[12], m, L[3]);
+      L[4] = m2l_fma(D[20], m, L[4]);
+      L[5] = m2l_fma(D[21], m, L[5]);
+      L[6] = m2l_fma(D[22], m, L[6]);
+      L[7] = m2l_fma(D[23], m, L[7]);
+      L[8] = m2l_fma(D[24], m, L[8]);
+      L[9] = m2l_fma(D[25], m, L[9]);
     }
-    { const float m = -__ldg(Ms + 11) * rp;
-      L[1] = fmaf(D[21], m, L[1]);
-      L[2] = fmaf(D[23], m, L[2]);
-      L[3] = fmaf(D[24], m, L[3]);
+    { const T m = __ldg(Ms + 5) * rp;
+      L[1] = m2l_fma(D[11], m, L[1]);
+      L[2] = m2l_fma(D[13], m, L[2]);
+      L[3] = m2l_fma(D[14], m, L[3]);
+      L[4] = m2l_fma(D[21], m, L[4]);
+      L[5] = m2l_fma(D[23], m, L[5]);
+      L[6] = m2l_fma(D[24], m, L[6]);
+      L[7] = m2l_fma(D[26], m, L[7]);
+      L[8] = m2l_fma(D[27], m, L[8]);
+      L[9] = m2l_fma(D[28], m, L[9]);
     }
-    { const float m = -__ldg(Ms + 12) * rp;
-      L[1] = fmaf(D[22], m, L[1]);
-      L[2] = fmaf(D[24], m, L[2]);
-      L[3] = fmaf(D[25], m, L[3]);
+    { const T m = __ldg(Ms + 6) * rp;
+      L[1] = m2l_fma(D[12], m, L[1]);
+      L[2] = m2l_fma(D[14], m, L[2]);
+      L[3] = m2l_fma(D[15], m, L[3]);
+      L[4] = m2l_fma(D[22], m, L[4]);
+      L[5] = m2l_fma(D[24], m, L[5]);
+      L[6] = m2l_fma(D[25], m, L[6]);
+      L[7] = m2l_fma(D[27], m, L[7]);
+      L[8] = m2l_fma(D[28], m, L[8]);
+      L[9] = m2l_fma(D[29], m, L[9]);
     }
-    { const float m = -__ldg(Ms + 13) * rp;
-      L[1] = fmaf(D[23], m, L[1]);
-      L[2] = fmaf(D[26], m, L[2]);
-      L[3] = fmaf(D[27], m, L[3]);
+    { const T m = __ldg(Ms + 7) * rp;
+      L[1] = m2l_fma(D[13], m, L[1]);
+      L[2] = m2l_fma(D[16], m, L[2]);
+      L[3] = m2l_fma(D[17], m, L[3]);
+      L[4] = m2l_fma(D[23], m, L[4]);
+      L[5] = m2l_fma(D[26], m, L[5]);
+      L[6] = m2l_fma(D[27], m, L[6]);
+      L[7] = m2l_fma(D[30], m, L[7]);
+      L[8] = m2l_fma(D[31], m, L[8]);
+      L[9] = m2l_fma(D[32], m, L[9]);
     }
-    { const float m = -__ldg(Ms + 14) * rp;
-      L[1] = fmaf(D[24], m, L[1]);
-      L[2] = fmaf(D[27], m, L[2]);
-      L[3] = fmaf(D[28], m, L[3]);
+    { const T m = __ldg(Ms + 8) * rp;
+      L[1] = m2l_fma(D[14], m, L[1]);
+      L[2] = m2l_fma(D[17], m, L[2]);
+      L[3] = m2l_fma(D[18], m, L[3]);
+      L[4] = m2l_fma(D[24], m, L[4]);
+      L[5] = m2l_fma(D[27], m, L[5]);
+      L[6] = m2l_fma(D[28], m, L[6]);
+      L[7] = m2l_fma(D[31], m, L[7]);
+      L[8] = m2l_fma(D[32], m, L[8]);
+      L[9] = m2l_fma(D[33], m, L[9]);
     }
-    { const float m = -__ldg(Ms + 15) * rp;
-      L[1] = fmaf(D[25], m, L[1]);
-      L[2] = fmaf(D[28], m, L[2]);
-      L[3] = fmaf(D[29], m, L[3]);
+    { const T m = __ldg(Ms + 9) * rp;
+      L[1] = m2l_fma(D[15], m, L[1]);
+      L[2] = m2l_fma(D[18], m, L[2]);
+      L[3] = m2l_fma(D[19], m, L[3]);
+      L[4] = m2l_fma(D[25], m, L[4]);
+      L[5] = m2l_fma(D[28], m, L[5]);
+      L[6] = m2l_fma(D[29], m, L[6]);
+      L[7] = m2l_fma(D[32], m, L[7]);
+      L[8] = m2l_fma(D[33], m, L[8]);
+      L[9] = m2l_fma(D[34], m, L[9]);
     }
-    { const float m = -__ldg(Ms + 16) * rp;
-      L[1] = fmaf(D[26], m, L[1]);
-      L[2] = fmaf(D[30], m, L[2]);
-      L[3] = fmaf(D[31], m, L[3]);
+    rp *= rho;
+    { const T m = -__ldg(Ms + 10) * rp;
+      L[1] = m2l_fma(D[20], m, L[1]);
+      L[2] = m2l_fma(D[21], m, L[2]);
+      L[3] = m2l_fma(D[22], m, L[3]);
     }
-    { const float m = -__ldg(Ms + 17) * rp;
-      L[1] = fmaf(D[27], m, L[1]);
-      L[2] = fmaf(D[31], m, L[2]);
-      L[3] = fmaf(D[32], m, L[3]);
+    { const T m = -__ldg(Ms + 11) * rp;
+      L[1] = m2l_fma(D[21], m, L[1]);
+      L[2] = m2l_fma(D[23], m, L[2]);
+      L[3] = m2l_fma(D[24], m, L[3]);
     }
-    { const float m = -__ldg(Ms + 18) * rp;
-      L[1] = fmaf(D[28], m, L[1]);
-      L[2] = fmaf(D[32], m, L[2]);
-      L[3] = fmaf(D[33], m, L[3]);
+    { const T m = -__ldg(Ms + 12) * rp;
+      L[1] = m2l_fma(D[22], m, L[1]);
+      L[2] = m2l_fma(D[24], m, L[2]);
+      L[3] = m2l_fma(D[25], m, L[3]);
     }
-    { const float m = -__ldg(Ms + 19) * rp;
-      L[1] = fmaf(D[29], m, L[1]);
-      L[2] = fmaf(D[33], m, L[2]);
-      L[3] = fmaf(D[34], m, L[3]);
+    { const T m = -__ldg(Ms + 13) * rp;
+      L[1] = m2l_fma(D[23], m, L[1]);
+      L[2] = m2l_fma(D[26], m, L[2]);
+      L[3] = m2l_fma(D[27], m, L[3]);
+    }
+    { const T m = -__ldg(Ms + 14) * rp;
+      L[1] = m2l_fma(D[24], m, L[1]);
+      L[2] = m2l_fma(D[27], m, L[2]);
+      L[3] = m2l_fma(D[28], m, L[3]);
+    }
+    { const T m = -__ldg(Ms + 15) * rp;
+      L[1] = m2l_fma(D[25], m, L[1]);
+      L[2] = m2l_fma(D[28], m, L[2]);
+      L[3] = m2l_fma(D[29], m, L[3]);
+    }
+    { const T m = -__ldg(Ms + 16) * rp;
+      L[1] = m2l_fma(D[26], m, L[1]);
+      L[2] = m2l_fma(D[30], m, L[2]);
+      L[3] = m2l_fma(D[31], m, L[3]);
+    }
+    { const T m = -__ldg(Ms + 17) * rp;
+      L[1] = m2l_fma(D[27], m, L[1]);
+      L[2] = m2l_fma(D[31], m, L[2]);
+      L[3] = m2l_fma(D[32], m, L[3]);
+    }
+    { const T m = -__ldg(Ms + 18) * rp;
+      L[1] = m2l_fma(D[28], m, L[1]);
+      L[2] = m2l_fma(D[32], m, L[2]);
+      L[3] = m2l_fma(D[33], m, L[3]);
+    }
+    { const T m = -__ldg(Ms + 19) * rp;
+      L[1] = m2l_fma(D[29], m, L[1]);
+      L[2] = m2l_fma(D[33], m, L[2]);
+      L[3] = m2l_fma(D[34], m, L[3]);
     }
 }
 
-__device__ __forceinline__ void m2l_side_b_forces_4(const float (&D)[35], const float *__restrict__ Ms, float (&L)[35])
+template <class T> __device__ __forceinline__ void m2l_side_b_forces_4(const T (&D)[35], const T *__restrict__ Ms, T (&L)[35])
 {
-    L[0] = 0.0f;
-    { const float m = __ldg(Ms + 0);
+    L[0] = T(0);
+    { const T m = __ldg(Ms + 0);
       L[1] = -D[1] * m;
       L[2] = -D[2] * m;
       L[3] = -D[3] * m;
@@ -1750,325 +1757,324 @@ __device__ __forceinline__ void m2l_side_b_forces_4(const float (&D)[35], const 
       L[33] = D[33] * m;
       L[34] = D[34] * m;
     }
-    { const float m = __ldg(Ms + 1);
-      L[1] = fmaf(-D[4], m, L[1]);
-      L[2] = fmaf(-D[5], m, L[2]);
-      L[3] = fmaf(-D[6], m, L[3]);
-      L[4] = fmaf(D[10], m, L[4]);
-      L[5] = fmaf(D[11], m, L[5]);
-      L[6] = fmaf(D[12], m, L[6]);
-      L[7] = fmaf(D[13], m, L[7]);
-      L[8] = fmaf(D[14], m, L[8]);
-      L[9] = fmaf(D[15], m, L[9]);
-      L[10] = fmaf(-D[20], m, L[10]);
-      L[11] = fmaf(-D[21], m, L[11]);
-      L[12] = fmaf(-D[22], m, L[12]);
-      L[13] = fmaf(-D[23], m, L[13]);
-      L[14] = fmaf(-D[24], m, L[14]);
-      L[15] = fmaf(-D[25], m, L[15]);
-      L[16] = fmaf(-D[26], m, L[16]);
-      L[17] = fmaf(-D[27], m, L[17]);
-      L[18] = fmaf(-D[28], m, L[18]);
-      L[19] = fmaf(-D[29], m, L[19]);
+    { const T m = __ldg(Ms + 1);
+      L[1] = m2l_fma(-D[4], m, L[1]);
+      L[2] = m2l_fma(-D[5], m, L[2]);
+      L[3] = m2l_fma(-D[6], m, L[3]);
+      L[4] = m2l_fma(D[10], m, L[4]);
+      L[5] = m2l_fma(D[11], m, L[5]);
+      L[6] = m2l_fma(D[12], m, L[6]);
+      L[7] = m2l_fma(D[13], m, L[7]);
+      L[8] = m2l_fma(D[14], m, L[8]);
+      L[9] = m2l_fma(D[15], m, L[9]);
+      L[10] = m2l_fma(-D[20], m, L[10]);
+      L[11] = m2l_fma(-D[21], m, L[11]);
+      L[12] = m2l_fma(-D[22], m, L[12]);
+      L[13] = m2l_fma(-D[23], m, L[13]);
+      L[14] = m2l_fma(-D[24], m, L[14]);
+      L[15] = m2l_fma(-D[25], m, L[15]);
+      L[16] = m2l_fma(-D[26], m, L[16]);
+      L[17] = m2l_fma(-D[27], m, L[17]);
+      L[18] = m2l_fma(-D[28], m, L[18]);
+      L[19] = m2l_fma(-D[29], m, L[19]);
     }
-    { const float m = __ldg(Ms + 2);
-      L[1] = fmaf(-D[5], m, L[1]);
-      L[2] = fmaf(-D[7], m, L[2]);
-      L[3] = fmaf(-D[8], m, L[3]);
-      L[4] = fmaf(D[11], m, L[4]);
-      L[5] = fmaf(D[13], m, L[5]);
-      L[6] = fmaf(D[14], m, L[6]);
-      L[7] = fmaf(D[16], m, L[7]);
-      L[8] = fmaf(D[17], m, L[8]);
-      L[9] = fmaf(D[18], m, L[9]);
-      L[10] = fmaf(-D[21], m, L[10]);
-      L[11] = fmaf(-D[23], m, L[11]);
-      L[12] = fmaf(-D[24], m, L[12]);
-      L[13] = fmaf(-D[26], m, L[13]);
-      L[14] = fmaf(-D[27], m, L[14]);
-      L[15] = fmaf(-D[28], m, L[15]);
-      L[16] = fmaf(-D[30], m, L[16]);
-      L[17] = fmaf(-D[31], m, L[17]);
-      L[18] = fmaf(-D[32], m, L[18]);
-      L[19] = fmaf(-D[33], m, L[19]);
+    { const T m = __ldg(Ms + 2);
+      L[1] = m2l_fma(-D[5], m, L[1]);
+      L[2] = m2l_fma(-D[7], m, L[2]);
+      L[3] = m2l_fma(-D[8], m, L[3]);
+      L[4] = m2l_fma(D[11], m, L[4]);
+      L[5] = m2l_fma(D[13], m, L[5]);
+      L[6] = m2l_fma(D[14], m, L[6]);
+      L[7] = m2l_fma(D[16], m, L[7]);
+      L[8] = m2l_fma(D[17], m, L[8]);
+      L[9] = m2l_fma(D[18], m, L[9]);
+      L[10] = m2l_fma(-D[21], m, L[10]);
+      L[11] = m2l_fma(-D[23], m, L[11]);
+      L[12] = m2l_fma(-D[24], m, L[12]);
+      L[13] = m2l_fma(-D[26], m, L[13]);
+      L[14] = m2l_fma(-D[27], m, L[14]);
+      L[15] = m2l_fma(-D[28], m, L[15]);
+      L[16] = m2l_fma(-D[30], m, L[16]);
+      L[17] = m2l_fma(-D[31], m, L[17]);
+      L[18] = m2l_fma(-D[32], m, L[18]);
+      L[19] = m2l_fma(-D[33], m, L[19]);
     }
-    { const float m = __ldg(Ms + 3);
-      L[1] = fmaf(-D[6], m, L[1]);
-      L[2] = fmaf(-D[8], m, L[2]);
-      L[3] = fmaf(-D[9], m, L[3]);
-      L[4] = fmaf(D[12], m, L[4]);
-      L[5] = fmaf(D[14], m, L[5]);
-      L[6] = fmaf(D[15], m, L[6]);
-      L[7] = fmaf(D[17], m, L[7]);
-      L[8] = fmaf(D[18], m, L[8]);
-      L[9] = fmaf(D[19], m, L[9]);
-      L[10] = fmaf(-D[22], m, L[10]);
-      L[11] = fmaf(-D[24], m, L[11]);
-      L[12] = fmaf(-D[25], m, L[12]);
-      L[13] = fmaf(-D[27], m, L[13]);
-      L[14] = fmaf(-D[28], m, L[14]);
-      L[15] = fmaf(-D[29], m, L[15]);
-      L[16] = fmaf(-D[31], m, L[16]);
-      L[17] = fmaf(-D[32], m, L[17]);
-      L[18] = fmaf(-D[33], m, L[18]);
-      L[19] = fmaf(-D[34], m, L[19]);
+    { const T m = __ldg(Ms + 3);
+      L[1] = m2l_fma(-D[6], m, L[1]);
+      L[2] = m2l_fma(-D[8], m, L[2]);
+      L[3] = m2l_fma(-D[9], m, L[3]);
+      L[4] = m2l_fma(D[12], m, L[4]);
+      L[5] = m2l_fma(D[14], m, L[5]);
+      L[6] = m2l_fma(D[15], m, L[6]);
+      L[7] = m2l_fma(D[17], m, L[7]);
+      L[8] = m2l_fma(D[18], m, L[8]);
+      L[9] = m2l_fma(D[19], m, L[9]);
+      L[10] = m2l_fma(-D[22], m, L[10]);
+      L[11] = m2l_fma(-D[24], m, L[11]);
+      L[12] = m2l_fma(-D[25], m, L[12]);
+      L[13] = m2l_fma(-D[27], m, L[13]);
+      L[14] = m2l_fma(-D[28], m, L[14]);
+      L[15] = m2l_fma(-D[29], m, L[15]);
+      L[16] = m2l_fma(-D[31], m, L[16]);
+      L[17] = m2l_fma(-D[32], m, L[17]);
+      L[18] = m2l_fma(-D[33], m, L[18]);
+      L[19] = m2l_fma(-D[34], m, L[19]);
     }
-    { const float m = __ldg(Ms + 4);
-      L[1] = fmaf(-D[10], m, L[1]);
-      L[2] = fmaf(-D[11], m, L[2]);
-      L[3] = fmaf(-D[12], m, L[3]);
-      L[4] = fmaf(D[20], m, L[4]);
-      L[5] = fmaf(D[21], m, L[5]);
-      L[6] = fmaf(D[22], m, L[6]);
-      L[7] = fmaf(D[23], m, L[7]);
-      L[8] = fmaf(D[24], m, L[8]);
-      L[9] = fmaf(D[25], m, L[9]);
+    { const T m = __ldg(Ms + 4);
+      L[1] = m2l_fma(-D[10], m, L[1]);
+      L[2] = m2l_fma(-D[11], m, L[2]);
+      L[3] = m2l_fma(-D[12], m, L[3]);
+      L[4] = m2l_fma(D[20], m, L[4]);
+      L[5] = m2l_fma(D[21], m, L[5]);
+      L[6] = m2l_fma(D[22], m, L[6]);
+      L[7] = m2l_fma(D[23], m, L[7]);
+      L[8] = m2l_fma(D[24], m, L[8]);
+      L[9] = m2l_fma(D[25], m, L[9]);
     }
-    { const float m = __ldg(Ms + 5);
-      L[1] = fmaf(-D[11], m, L[1]);
-      L[2] = fmaf(-D[13], m, L[2]);
-      L[3] = fmaf(-D[14], m, L[3]);
-      L[4] = fmaf(D[21], m, L[4]);
-      L[5] = fmaf(D[23], m, L[5]);
-      L[6] = fmaf(D[24], m, L[6]);
-      L[7] = fmaf(D[26], m, L[7]);
-      L[8] = fmaf(D[27], m, L[8]);
-      L[9] = fmaf(D[28], m, L[9]);
+    { const T m = __ldg(Ms + 5);
+      L[1] = m2l_fma(-D[11], m, L[1]);
+      L[2] = m2l_fma(-D[13], m, L[2]);
+      L[3] = m2l_fma(-D[14], m, L[3]);
+      L[4] = m2l_fma(D[21], m, L[4]);
+      L[5] = m2l_fma(D[23], m, L[5]);
+      L[6] = m2l_fma(D[24], m, L[6]);
+      L[7] = m2l_fma(D[26], m, L[7]);
+      L[8] = m2l_fma(D[27], m, L[8]);
+      L[9] = m2l_fma(D[28], m, L[9]);
     }
-    { const float m = __ldg(Ms + 6);
-      L[1] = fmaf(-D[12], m, L[1]);
-      L[2] = fmaf(-D[14], m, L[2]);
-      L[3] = fmaf(-D[15], m, L[3]);
-      L[4] = fmaf(D[22], m, L[4]);
-      L[5] = fmaf(D[24], m, L[5]);
-      L[6] = fmaf(D[25], m, L[6]);
-      L[7] = fmaf(D[27], m, L[7]);
-      L[8] = fmaf(D[28], m, L[8]);
-      L[9] = fmaf(D[29], m, L[9]);
+    { const T m = __ldg(Ms + 6);
+      L[1] = m2l_fma(-D[12], m, L[1]);
+      L[2] = m2l_fma(-D[14], m, L[2]);
+      L[3] = m2l_fma(-D[15], m, L[3]);
+      L[4] = m2l_fma(D[22], m, L[4]);
+      L[5] = m2l_fma(D[24], m, L[5]);
+      L[6] = m2l_fma(D[25], m, L[6]);
+      L[7] = m2l_fma(D[27], m, L[7]);
+      L[8] = m2l_fma(D[28], m, L[8]);
+      L[9] = m2l_fma(D[29], m, L[9]);
     }
-    { const float m = __ldg(Ms + 7);
-      L[1] = fmaf(-D[13], m, L[1]);
-      L[2] = fmaf(-D[16], m, L[2]);
-      L[3] = fmaf(-D[17], m, L[3]);
-      L[4] = fmaf(D[23], m, L[4]);
-      L[5] = fmaf(D[26], m, L[5]);
-      L[6] = fmaf(D[27], m, L[6]);
-      L[7] = fmaf(D[30], m, L[7]);
-      L[8] = fmaf(D[31], m, L[8]);
-      L[9] = fmaf(D[32], m, L[9]);
+    { const T m = __ldg(Ms + 7);
+      L[1] = m2l_fma(-D[13], m, L[1]);
+      L[2] = m2l_fma(-D[16], m, L[2]);
+      L[3] = m2l_fma(-D[17], m, L[3]);
+      L[4] = m2l_fma(D[23], m, L[4]);
+      L[5] = m2l_fma(D[26], m, L[5]);
+      L[6] = m2l_fma(D[27], m, L[6]);
+      L[7] = m2l_fma(D[30], m, L[7]);
+      L[8] = m2l_fma(D[31], m, L[8]);
+      L[9] = m2l_fma(D[32], m, L[9]);
     }
-    { const float m = __ldg(Ms + 8);
-      L[1] = fmaf(-D[14], m, L[1]);
-      L[2] = fmaf(-D[17], m, L[2]);
-      L[3] = fmaf(-D[18], m, L[3]);
-      L[4] = fmaf(D[24], m, L[4]);
-      L[5] = fmaf(D[27], m, L[5]);
-      L[6] = fmaf(D[28], m, L[6]);
-      L[7] = fmaf(D[31], m, L[7]);
-      L[8] = fmaf(D[32], m, L[8]);
-      L[9] = fmaf(D[33], m, L[9]);
+    { const T m = __ldg(Ms + 8);
+      L[1] = m2l_fma(-D[14], m, L[1]);
+      L[2] = m2l_fma(-D[17], m, L[2]);
+      L[3] = m2l_fma(-D[18], m, L[3]);
+      L[4] = m2l_fma(D[24], m, L[4]);
+      L[5] = m2l_fma(D[27], m, L[5]);
+      L[6] = m2l_fma(D[28], m, L[6]);
+      L[7] = m2l_fma(D[31], m, L[7]);
+      L[8] = m2l_fma(D[32], m, L[8]);
+      L[9] = m2l_fma(D[33], m, L[9]);
     }
-    { const float m = __ldg(Ms + 9);
-      L[1] = fmaf(-D[15], m, L[1]);
-      L[2] = fmaf(-D[18], m, L[2]);
-      L[3] = fmaf(-D[19], m, L[3]);
-      L[4] = fmaf(D[25], m, L[4]);
-      L[5] = fmaf(D[28], m, L[5]);
-      L[6] = fmaf(D[29], m, L[6]);
-      L[7] = fmaf(D[32], m, L[7]);
-      L[8] = fmaf(D[33], m, L[8]);
-      L[9] = fmaf(D[34], m, L[9]);
+    { const T m = __ldg(Ms + 9);
+      L[1] = m2l_fma(-D[15], m, L[1]);
+      L[2] = m2l_fma(-D[18], m, L[2]);
+      L[3] = m2l_fma(-D[19], m, L[3]);
+      L[4] = m2l_fma(D[25], m, L[4]);
+      L[5] = m2l_fma(D[28], m, L[5]);
+      L[6] = m2l_fma(D[29], m, L[6]);
+      L[7] = m2l_fma(D[32], m, L[7]);
+      L[8] = m2l_fma(D[33], m, L[8]);
+      L[9] = m2l_fma(D[34], m, L[9]);
     }
-    { const float m = __ldg(Ms + 10);
-      L[1] = fmaf(-D[20], m, L[1]);
-      L[2] = fmaf(-D[21], m, L[2]);
-      L[3] = fmaf(-D[22], m, L[3]);
+    { const T m = __ldg(Ms + 10);
+      L[1] = m2l_fma(-D[20], m, L[1]);
+      L[2] = m2l_fma(-D[21], m, L[2]);
+      L[3] = m2l_fma(-D[22], m, L[3]);
     }
-    { const float m = __ldg(Ms + 11);
-      L[1] = fmaf(-D[21], m, L[1]);
-      L[2] = fmaf(-D[23], m, L[2]);
-      L[3] = fmaf(-D[24], m, L[3]);
+    { const T m = __ldg(Ms + 11);
+      L[1] = m2l_fma(-D[21], m, L[1]);
+      L[2] = m2l_fma(-D[23], m, L[2]);
+      L[3] = m2l_fma(-D[24], m, L[3]);
     }
-    { const float m = __ldg(Ms + 12);
-      L[1] = fmaf(-D[22], m, L[1]);
-      L[2] = fmaf(-D[24], m, L[2]);
-      L[3] = fmaf(-D[25], m, L[3]);
+    { const T m = __ldg(Ms + 12);
+      L[1] = m2l_fma(-D[22], m, L[1]);
+      L[2] = m2l_fma(-D[24], m, L[2]);
+      L[3] = m2l_fma(-D[25], m, L[3]);
     }
-    { const float m = __ldg(Ms + 13);
-      L[1] = fmaf(-D[23], m, L[1]);
-      L[2] = fmaf(-D[26], m, L[2]);
-      L[3] = fmaf(-D[27], m, L[3]);
+    { const T m = __ldg(Ms + 13);
+      L[1] = m2l_fma(-D[23], m, L[1]);
+      L[2] = m2l_fma(-D[26], m, L[2]);
+      L[3] = m2l_fma(-D[27], m, L[3]);
     }
-    { const float m = __ldg(Ms + 14);
-      L[1] = fmaf(-D[24], m, L[1]);
-      L[2] = fmaf(-D[27], m, L[2]);
-      L[3] = fmaf(-D[28], m, L[3]);
+    { const T m = __ldg(Ms + 14);
+      L[1] = m2l_fma(-D[24], m, L[1]);
+      L[2] = m2l_fma(-D[27], m, L[2]);
+      L[3] = m2l_fma(-D[28], m, L[3]);
     }
-    { const float m = __ldg(Ms + 15);
-      L[1] = fmaf(-D[25], m, L[1]);
-      L[2] = fmaf(-D[28], m, L[2]);
-      L[3] = fmaf(-D[29], m, L[3]);
+    { const T m = __ldg(Ms + 15);
+      L[1] = m2l_fma(-D[25], m, L[1]);
+      L[2] = m2l_fma(-D[28], m, L[2]);
+      L[3] = m2l_fma(-D[29], m, L[3]);
     }
-    { const float m = __ldg(Ms + 16);
-      L[1] = fmaf(-D[26], m, L[1]);
-      L[2] = fmaf(-D[30], m, L[2]);
-      L[3] = fmaf(-D[31], m, L[3]);
+    { const T m = __ldg(Ms + 16);
+      L[1] = m2l_fma(-D[26], m, L[1]);
+      L[2] = m2l_fma(-D[30], m, L[2]);
+      L[3] = m2l_fma(-D[31], m, L[3]);
     }
-    { const float m = __ldg(Ms + 17);
-      L[1] = fmaf(-D[27], m, L[1]);
-      L[2] = fmaf(-D[31], m, L[2]);
-      L[3] = fmaf(-D[32], m, L[3]);
+    { const T m = __ldg(Ms + 17);
+      L[1] = m2l_fma(-D[27], m, L[1]);
+      L[2] = m2l_fma(-D[31], m, L[2]);
+      L[3] = m2l_fma(-D[32], m, L[3]);
     }
-    { const float m = __ldg(Ms + 18);
-      L[1] = fmaf(-D[28], m, L[1]);
-      L[2] = fmaf(-D[32], m, L[2]);
-      L[3] = fmaf(-D[33], m, L[3]);
+    { const T m = __ldg(Ms + 18);
+      L[1] = m2l_fma(-D[28], m, L[1]);
+      L[2] = m2l_fma(-D[32], m, L[2]);
+      L[3] = m2l_fma(-D[33], m, L[3]);
     }
-    { const float m = __ldg(Ms + 19);
-      L[1] = fmaf(-D[29], m, L[1]);
-      L[2] = fmaf(-D[33], m, L[2]);
-      L[3] = fmaf(-D[34], m, L[3]);
+    { const T m = __ldg(Ms + 19);
+      L[1] = m2l_fma(-D[29], m, L[1]);
+      L[2] = m2l_fma(-D[33], m, L[2]);
+      L[3] = m2l_fma(-D[34], m, L[3]);
     }
 }
 
-__device__ __forceinline__ void m2l_dtensor_5(float dx, float dy, float dz, float soft2, float (&D)[56])
+template <class T> __device__ __forceinline__ void m2l_dtensor_5(T dx, T dy, T dz, T soft2, T (&D)[56])
 {
-    const float s2 = fmaf(dx, dx, fmaf(dy, dy, fmaf(dz, dz, soft2)));
-    float si = rsqrtf(s2);
-    si = si * fmaf(-0.5f * s2, si * si, 1.5f);   // one Newton step
-    const float si2 = si * si;
-    const float f0 = -si;
-    const float f1 = -1.0f * f0 * si2;
-    const float f2 = -3.0f * f1 * si2;
-    const float f3 = -5.0f * f2 * si2;
-    const float f4 = -7.0f * f3 * si2;
-    const float f5 = -9.0f * f4 * si2;
-    const float r_0_0 = f0;
-    const float r_1_0 = f1;
-    const float r_2_0 = f2;
-    const float r_3_0 = f3;
-    const float r_4_0 = f4;
-    const float r_5_0 = f5;
-    const float r_0_1 = dx * r_1_0;
-    const float r_1_1 = dx * r_2_0;
-    const float r_2_1 = dx * r_3_0;
-    const float r_3_1 = dx * r_4_0;
-    const float r_4_1 = dx * r_5_0;
-    const float r_0_2 = dy * r_1_0;
-    const float r_1_2 = dy * r_2_0;
-    const float r_2_2 = dy * r_3_0;
-    const float r_3_2 = dy * r_4_0;
-    const float r_4_2 = dy * r_5_0;
-    const float r_0_3 = dz * r_1_0;
-    const float r_1_3 = dz * r_2_0;
-    const float r_2_3 = dz * r_3_0;
-    const float r_3_3 = dz * r_4_0;
-    const float r_4_3 = dz * r_5_0;
-    const float r_0_4 = fmaf(1.0f, r_1_0, dx * r_1_1);
-    const float r_1_4 = fmaf(1.0f, r_2_0, dx * r_2_1);
-    const float r_2_4 = fmaf(1.0f, r_3_0, dx * r_3_1);
-    const float r_3_4 = fmaf(1.0f, r_4_0, dx * r_4_1);
-    const float r_0_5 = dx * r_1_2;
-    const float r_1_5 = dx * r_2_2;
-    const float r_2_5 = dx * r_3_2;
-    const float r_3_5 = dx * r_4_2;
-    const float r_0_6 = dx * r_1_3;
-    const float r_1_6 = dx * r_2_3;
-    const float r_2_6 = dx * r_3_3;
-    const float r_3_6 = dx * r_4_3;
-    const float r_0_7 = fmaf(1.0f, r_1_0, dy * r_1_2);
-    const float r_1_7 = fmaf(1.0f, r_2_0, dy * r_2_2);
-    const float r_2_7 = fmaf(1.0f, r_3_0, dy * r_3_2);
-    const float r_3_7 = fmaf(1.0f, r_4_0, dy * r_4_2);
-    const float r_0_8 = dy * r_1_3;
-    const float r_1_8 = dy * r_2_3;
-    const float r_2_8 = dy * r_3_3;
-    const float r_3_8 = dy * r_4_3;
-    const float r_0_9 = fmaf(1.0f, r_1_0, dz * r_1_3);
-    const float r_1_9 = fmaf(1.0f, r_2_0, dz * r_2_3);
-    const float r_2_9 = fmaf(1.0f, r_3_0, dz * r_3_3);
-    const float r_3_9 = fmaf(1.0f, r_4_0, dz * r_4_3);
-    const float r_0_10 = fmaf(2.0f, r_1_1, dx * r_1_4);
-    const float r_1_10 = fmaf(2.0f, r_2_1, dx * r_2_4);
-    const float r_2_10 = fmaf(2.0f, r_3_1, dx * r_3_4);
-    const float r_0_11 = fmaf(1.0f, r_1_2, dx * r_1_5);
-    const float r_1_11 = fmaf(1.0f, r_2_2, dx * r_2_5);
-    const float r_2_11 = fmaf(1.0f, r_3_2, dx * r_3_5);
-    const float r_0_12 = fmaf(1.0f, r_1_3, dx * r_1_6);
-    const float r_1_12 = fmaf(1.0f, r_2_3, dx * r_2_6);
-    const float r_2_12 = fmaf(1.0f, r_3_3, dx * r_3_6);
-    const float r_0_13 = dx * r_1_7;
-    const float r_1_13 = dx * r_2_7;
-    const float r_2_13 = dx * r_3_7;
-    const float r_0_14 = dx * r_1_8;
-    const float r_1_14 = dx * r_2_8;
-    const float r_2_14 = dx * r_3_8;
-    const float r_0_15 = dx * r_1_9;
-    const float r_1_15 = dx * r_2_9;
-    const float r_2_15 = dx * r_3_9;
-    const float r_0_16 = fmaf(2.0f, r_1_2, dy * r_1_7);
-    const float r_1_16 = fmaf(2.0f, r_2_2, dy * r_2_7);
-    const float r_2_16 = fmaf(2.0f, r_3_2, dy * r_3_7);
-    const float r_0_17 = fmaf(1.0f, r_1_3, dy * r_1_8);
-    const float r_1_17 = fmaf(1.0f, r_2_3, dy * r_2_8);
-    const float r_2_17 = fmaf(1.0f, r_3_3, dy * r_3_8);
-    const float r_0_18 = dy * r_1_9;
-    const float r_1_18 = dy * r_2_9;
-    const float r_2_18 = dy * r_3_9;
-    const float r_0_19 = fmaf(2.0f, r_1_3, dz * r_1_9);
-    const float r_1_19 = fmaf(2.0f, r_2_3, dz * r_2_9);
-    const float r_2_19 = fmaf(2.0f, r_3_3, dz * r_3_9);
-    const float r_0_20 = fmaf(3.0f, r_1_4, dx * r_1_10);
-    const float r_1_20 = fmaf(3.0f, r_2_4, dx * r_2_10);
-    const float r_0_21 = fmaf(2.0f, r_1_5, dx * r_1_11);
-    const float r_1_21 = fmaf(2.0f, r_2_5, dx * r_2_11);
-    const float r_0_22 = fmaf(2.0f, r_1_6, dx * r_1_12);
-    const float r_1_22 = fmaf(2.0f, r_2_6, dx * r_2_12);
-    const float r_0_23 = fmaf(1.0f, r_1_7, dx * r_1_13);
-    const float r_1_23 = fmaf(1.0f, r_2_7, dx * r_2_13);
-    const float r_0_24 = fmaf(1.0f, r_1_8, dx * r_1_14);
-    const float r_1_24 = fmaf(1.0f, r_2_8, dx * r_2_14);
-    const float r_0_25 = fmaf(1.0f, r_1_9, dx * r_1_15);
-    const float r_1_25 = fmaf(1.0f, r_2_9, dx * r_2_15);
-    const float r_0_26 = dx * r_1_16;
-    const float r_1_26 = dx * r_2_16;
-    const float r_0_27 = dx * r_1_17;
-    const float r_1_27 = dx * r_2_17;
-    const float r_0_28 = dx * r_1_18;
-    const float r_1_28 = dx * r_2_18;
-    const float r_0_29 = dx * r_1_19;
-    const float r_1_29 = dx * r_2_19;
-    const float r_0_30 = fmaf(3.0f, r_1_7, dy * r_1_16);
-    const float r_1_30 = fmaf(3.0f, r_2_7, dy * r_2_16);
-    const float r_0_31 = fmaf(2.0f, r_1_8, dy * r_1_17);
-    const float r_1_31 = fmaf(2.0f, r_2_8, dy * r_2_17);
-    const float r_0_32 = fmaf(1.0f, r_1_9, dy * r_1_18);
-    const float r_1_32 = fmaf(1.0f, r_2_9, dy * r_2_18);
-    const float r_0_33 = dy * r_1_19;
-    const float r_1_33 = dy * r_2_19;
-    const float r_0_34 = fmaf(3.0f, r_1_9, dz * r_1_19);
-    const float r_1_34 = fmaf(3.0f, r_2_9, dz * r_2_19);
-    const float r_0_35 = fmaf(4.0f, r_1_10, dx * r_1_20);
-    const float r_0_36 = fmaf(3.0f, r_1_11, dx * r_1_21);
-    const float r_0_37 = fmaf(3.0f, r_1_12, dx * r_1_22);
-    const float r_0_38 = fmaf(2.0f, r_1_13, dx * r_1_23);
-    const float r_0_39 = fmaf(2.0f, r_1_14, dx * r_1_24);
-    const float r_0_40 = fmaf(2.0f, r_1_15, dx * r_1_25);
-    const float r_0_41 = fmaf(1.0f, r_1_16, dx * r_1_26);
-    const float r_0_42 = fmaf(1.0f, r_1_17, dx * r_1_27);
-    const float r_0_43 = fmaf(1.0f, r_1_18, dx * r_1_28);
-    const float r_0_44 = fmaf(1.0f, r_1_19, dx * r_1_29);
-    const float r_0_45 = dx * r_1_30;
-    const float r_0_46 = dx * r_1_31;
-    const float r_0_47 = dx * r_1_32;
-    const float r_0_48 = dx * r_1_33;
-    const float r_0_49 = dx * r_1_34;
-    const float r_0_50 = fmaf(4.0f, r_1_16, dy * r_1_30);
-    const float r_0_51 = fmaf(3.0f, r_1_17, dy * r_1_31);
-    const float r_0_52 = fmaf(2.0f, r_1_18, dy * r_1_32);
-    const float r_0_53 = fmaf(1.0f, r_1_19, dy * r_1_33);
-    const float r_0_54 = dy * r_1_34;
-    const float r_0_55 = fmaf(4.0f, r_1_19, dz * r_1_34);
+    const T s2 = m2l_fma(dx, dx, m2l_fma(dy, dy, m2l_fma(dz, dz, soft2)));
+    const T si = m2l_rsqrt(s2);
+    const T si2 = si * si;
+    const T f0 = -si;
+    const T f1 = T(-1) * f0 * si2;
+    const T f2 = T(-3) * f1 * si2;
+    const T f3 = T(-5) * f2 * si2;
+    const T f4 = T(-7) * f3 * si2;
+    const T f5 = T(-9) * f4 * si2;
+    const T r_0_0 = f0;
+    const T r_1_0 = f1;
+    const T r_2_0 = f2;
+    const T r_3_0 = f3;
+    const T r_4_0 = f4;
+    const T r_5_0 = f5;
+    const T r_0_1 = dx * r_1_0;
+    const T r_1_1 = dx * r_2_0;
+    const T r_2_1 = dx * r_3_0;
+    const T r_3_1 = dx * r_4_0;
+    const T r_4_1 = dx * r_5_0;
+    const T r_0_2 = dy * r_1_0;
+    const T r_1_2 = dy * r_2_0;
+    const T r_2_2 = dy * r_3_0;
+    const T r_3_2 = dy * r_4_0;
+    const T r_4_2 = dy * r_5_0;
+    const T r_0_3 = dz * r_1_0;
+    const T r_1_3 = dz * r_2_0;
+    const T r_2_3 = dz * r_3_0;
+    const T r_3_3 = dz * r_4_0;
+    const T r_4_3 = dz * r_5_0;
+    const T r_0_4 = m2l_fma(T(1), r_1_0, dx * r_1_1);
+    const T r_1_4 = m2l_fma(T(1), r_2_0, dx * r_2_1);
+    const T r_2_4 = m2l_fma(T(1), r_3_0, dx * r_3_1);
+    const T r_3_4 = m2l_fma(T(1), r_4_0, dx * r_4_1);
+    const T r_0_5 = dx * r_1_2;
+    const T r_1_5 = dx * r_2_2;
+    const T r_2_5 = dx * r_3_2;
+    const T r_3_5 = dx * r_4_2;
+    const T r_0_6 = dx * r_1_3;
+    const T r_1_6 = dx * r_2_3;
+    const T r_2_6 = dx * r_3_3;
+    const T r_3_6 = dx * r_4_3;
+    const T r_0_7 = m2l_fma(T(1), r_1_0, dy * r_1_2);
+    const T r_1_7 = m2l_fma(T(1), r_2_0, dy * r_2_2);
+    const T r_2_7 = m2l_fma(T(1), r_3_0, dy * r_3_2);
+    const T r_3_7 = m2l_fma(T(1), r_4_0, dy * r_4_2);
+    const T r_0_8 = dy * r_1_3;
+    const T r_1_8 = dy * r_2_3;
+    const T r_2_8 = dy * r_3_3;
+    const T r_3_8 = dy * r_4_3;
+    const T r_0_9 = m2l_fma(T(1), r_1_0, dz * r_1_3);
+    const T r_1_9 = m2l_fma(T(1), r_2_0, dz * r_2_3);
+    const T r_2_9 = m2l_fma(T(1), r_3_0, dz * r_3_3);
+    const T r_3_9 = m2l_fma(T(1), r_4_0, dz * r_4_3);
+    const T r_0_10 = m2l_fma(T(2), r_1_1, dx * r_1_4);
+    const T r_1_10 = m2l_fma(T(2), r_2_1, dx * r_2_4);
+    const T r_2_10 = m2l_fma(T(2), r_3_1, dx * r_3_4);
+    const T r_0_11 = m2l_fma(T(1), r_1_2, dx * r_1_5);
+    const T r_1_11 = m2l_fma(T(1), r_2_2, dx * r_2_5);
+    const T r_2_11 = m2l_fma(T(1), r_3_2, dx * r_3_5);
+    const T r_0_12 = m2l_fma(T(1), r_1_3, dx * r_1_6);
+    const T r_1_12 = m2l_fma(T(1), r_2_3, dx * r_2_6);
+    const T r_2_12 = m2l_fma(T(1), r_3_3, dx * r_3_6);
+    const T r_0_13 = dx * r_1_7;
+    const T r_1_13 = dx * r_2_7;
+    const T r_2_13 = dx * r_3_7;
+    const T r_0_14 = dx * r_1_8;
+    const T r_1_14 = dx * r_2_8;
+    const T r_2_14 = dx * r_3_8;
+    const T r_0_15 = dx * r_1_9;
+    const T r_1_15 = dx * r_2_9;
+    const T r_2_15 = dx * r_3_9;
+    const T r_0_16 = m2l_fma(T(2), r_1_2, dy * r_1_7);
+    const T r_1_16 = m2l_fma(T(2), r_2_2, dy * r_2_7);
+    const T r_2_16 = m2l_fma(T(2), r_3_2, dy * r_3_7);
+    const T r_0_17 = m2l_fma(T(1), r_1_3, dy * r_1_8);
+    const T r_1_17 = m2l_fma(T(1), r_2_3, dy * r_2_8);
+    const T r_2_17 = m2l_fma(T(1), r_3_3, dy * r_3_8);
+    const T r_0_18 = dy * r_1_9;
+    const T r_1_18 = dy * r_2_9;
+    const T r_2_18 = dy * r_3_9;
+    const T r_0_19 = m2l_fma(T(2), r_1_3, dz * r_1_9);
+    const T r_1_19 = m2l_fma(T(2), r_2_3, dz * r_2_9);
+    const T r_2_19 = m2l_fma(T(2), r_3_3, dz * r_3_9);
+    const T r_0_20 = m2l_fma(T(3), r_1_4, dx * r_1_10);
+    const T r_1_20 = m2l_fma(T(3), r_2_4, dx * r_2_10);
+    const T r_0_21 = m2l_fma(T(2), r_1_5, dx * r_1_11);
+    const T r_1_21 = m2l_fma(T(2), r_2_5, dx * r_2_11);
+    const T r_0_22 = m2l_fma(T(2), r_1_6, dx * r_1_12);
+    const T r_1_22 = m2l_fma(T(2), r_2_6, dx * r_2_12);
+    const T r_0_23 = m2l_fma(T(1), r_1_7, dx * r_1_13);
+    const T r_1_23 = m2l_fma(T(1), r_2_7, dx * r_2_13);
+    const T r_0_24 = m2l_fma(T(1), r_1_8, dx * r_1_14);
+    const T r_1_24 = m2l_fma(T(1), r_2_8, dx * r_2_14);
+    const T r_0_25 = m2l_fma(T(1), r_1_9, dx * r_1_15);
+    const T r_1_25 = m2l_fma(T(1), r_2_9, dx * r_2_15);
+    const T r_0_26 = dx * r_1_16;
+    const T r_1_26 = dx * r_2_16;
+    const T r_0_27 = dx * r_1_17;
+    const T r_1_27 = dx * r_2_17;
+    const T r_0_28 = dx * r_1_18;
+    const T r_1_28 = dx * r_2_18;
+    const T r_0_29 = dx * r_1_19;
+    const T r_1_29 = dx * r_2_19;
+    const T r_0_30 = m2l_fma(T(3), r_1_7, dy * r_1_16);
+    const T r_1_30 = m2l_fma(T(3), r_2_7, dy * r_2_16);
+    const T r_0_31 = m2l_fma(T(2), r_1_8, dy * r_1_17);
+    const T r_1_31 = m2l_fma(T(2), r_2_8, dy * r_2_17);
+    const T r_0_32 = m2l_fma(T(1), r_1_9, dy * r_1_18);
+    const T r_1_32 = m2l_fma(T(1), r_2_9, dy * r_2_18);
+    const T r_0_33 = dy * r_1_19;
+    const T r_1_33 = dy * r_2_19;
+    const T r_0_34 = m2l_fma(T(3), r_1_9, dz * r_1_19);
+    const T r_1_34 = m2l_fma(T(3), r_2_9, dz * r_2_19);
+    const T r_0_35 = m2l_fma(T(4), r_1_10, dx * r_1_20);
+    const T r_0_36 = m2l_fma(T(3), r_1_11, dx * r_1_21);
+    const T r_0_37 = m2l_fma(T(3), r_1_12, dx * r_1_22);
+    const T r_0_38 = m2l_fma(T(2), r_1_13, dx * r_1_23);
+    const T r_0_39 = m2l_fma(T(2), r_1_14, dx * r_1_24);
+    const T r_0_40 = m2l_fma(T(2), r_1_15, dx * r_1_25);
+    const T r_0_41 = m2l_fma(T(1), r_1_16, dx * r_1_26);
+    const T r_0_42 = m2l_fma(T(1), r_1_17, dx * r_1_27);
+    const T r_0_43 = m2l_fma(T(1), r_1_18, dx * r_1_28);
+    const T r_0_44 = m2l_fma(T(1), r_1_19, dx * r_1_29);
+    const T r_0_45 = dx * r_1_30;
+    const T r_0_46 = dx * r_1_31;
+    const T r_0_47 = dx * r_1_32;
+    const T r_0_48 = dx * r_1_33;
+    const T r_0_49 = dx * r_1_34;
+    const T r_0_50 = m2l_fma(T(4), r_1_16, dy * r_1_30);
+    const T r_0_51 = m2l_fma(T(3), r_1_17, dy * r_1_31);
+    const T r_0_52 = m2l_fma(T(2), r_1_18, dy * r_1_32);
+    const T r_0_53 = m2l_fma(T(1), r_1_19, dy * r_1_33);
+    const T r_0_54 = dy * r_1_34;
+    const T r_0_55 = m2l_fma(T(4), r_1_19, dz * r_1_34);
     D[0] = r_0_0;
     D[1] = r_0_1;
     D[2] = r_0_2;
@@ -2127,10 +2133,10 @@ __device__ __forceinline__ void m2l_dtensor_5(float dx, float dy, float dz, floa
     D[55] = r_0_55;
 }
 
-__device__ __forceinline__ void m2l_side_a_5(const float (&D)[56], const float *__restrict__ Ms, float rho, float (&L)[56])
+template <class T> __device__ __forceinline__ void m2l_side_a_5(const T (&D)[56], const T *__restrict__ Ms, T rho, T (&L)[56])
 {
-    float rp = 1.0f;
-    { const float m = __ldg(Ms + 0) * rp;
+    T rp = T(1);
+    { const T m = __ldg(Ms + 0) * rp;
       L[0] = D[0] * m;
       L[1] = D[1] * m;
       L[2] = D[2] * m;
@@ -2189,531 +2195,531 @@ __device__ __forceinline__ void m2l_side_a_5(const float (&D)[56], const float *
       L[55] = D[55] * m;
     }
     rp *= rho;
-    { const float m = -__ldg(Ms + 1) * rp;
-      L[0] = fmaf(D[1], m, L[0]);
-      L[1] = fmaf(D[4], m, L[1]);
-      L[2] = fmaf(D[5], m, L[2]);
-      L[3] = fmaf(D[6], m, L[3]);
-      L[4] = fmaf(D[10], m, L[4]);
-      L[5] = fmaf(D[11], m, L[5]);
-      L[6] = fmaf(D[12], m, L[6]);
-      L[7] = fmaf(D[13], m, L[7]);
-      L[8] = fmaf(D[14], m, L[8]);
-      L[9] = fmaf(D[15], m, L[9]);
-      L[10] = fmaf(D[20], m, L[10]);
-      L[11] = fmaf(D[21], m, L[11]);
-      L[12] = fmaf(D[22], m, L[12]);
-      L[13] = fmaf(D[23], m, L[13]);
-      L[14] = fmaf(D[24], m, L[14]);
-      L[15] = fmaf(D[25], m, L[15]);
-      L[16] = fmaf(D[26], m, L[16]);
-      L[17] = fmaf(D[27], m, L[17]);
-      L[18] = fmaf(D[28], m, L[18]);
-      L[19] = fmaf(D[29], m, L[19]);
-      L[20] = fmaf(D[35], m, L[20]);
-      L[21] = fmaf(D[36], m, L[21]);
-      L[22] = fmaf(D[37], m, L[22]);
-      L[23] = fmaf(D[38], m, L[23]);
-      L[24] = fmaf(D[39], m, L[24]);
-      L[25] = fmaf(D[40], m, L[25]);
-      L[26] = fmaf(D[41], m, L[26]);
-      L[27] = fmaf(D[42], m, L[27]);
-      L[28] = fmaf(D[43], m, L[28]);
-      L[29] = fmaf(D[44], m, L[29]);
-      L[30] = fmaf(D[45], m, L[30]);
-      L[31] = fmaf(D[46], m, L[31]);
-      L[32] = fmaf(D[47], m, L[32]);
-      L[33] = fmaf(D[48], m, L[33]);
-      L[34] = fmaf(D[49], m, L[34]);
+    { const T m = -__ldg(Ms + 1) * rp;
+      L[0] = m2l_fma(D[1], m, L[0]);
+      L[1] = m2l_fma(D[4], m, L[1]);
+      L[2] = m2l_fma(D[5], m, L[2]);
+      L[3] = m2l_fma(D[6], m, L[3]);
+      L[4] = m2l_fma(D[10], m, L[4]);
+      L[5] = m2l_fma(D[11], m, L[5]);
+      L[6] = m2l_fma(D[12], m, L[6]);
+      L[7] = m2l_fma(D[13], m, L[7]);
+      L[8] = m2l_fma(D[14], m, L[8]);
+      L[9] = m2l_fma(D[15], m, L[9]);
+      L[10] = m2l_fma(D[20], m, L[10]);
+      L[11] = m2l_fma(D[21], m, L[11]);
+      L[12] = m2l_fma(D[22], m, L[12]);
+      L[13] = m2l_fma(D[23], m, L[13]);
+      L[14] = m2l_fma(D[24], m, L[14]);
+      L[15] = m2l_fma(D[25], m, L[15]);
+      L[16] = m2l_fma(D[26], m, L[16]);
+      L[17] = m2l_fma(D[27], m, L[17]);
+      L[18] = m2l_fma(D[28], m, L[18]);
+      L[19] = m2l_fma(D[29], m, L[19]);
+      L[20] = m2l_fma(D[35], m, L[20]);
+      L[21] = m2l_fma(D[36], m, L[21]);
+      L[22] = m2l_fma(D[37], m, L[22]);
+      L[23] = m2l_fma(D[38], m, L[23]);
+      L[24] = m2l_fma(D[39], m, L[24]);
+      L[25] = m2l_fma(D[40], m, L[25]);
+      L[26] = m2l_fma(D[41], m, L[26]);
+      L[27] = m2l_fma(D[42], m, L[27]);
+      L[28] = m2l_fma(D[43], m, L[28]);
+      L[29] = m2l_fma(D[44], m, L[29]);
+      L[30] = m2l_fma(D[45], m, L[30]);
+      L[31] = m2l_fma(D[46], m, L[31]);
+      L[32] = m2l_fma(D[47], m, L[32]);
+      L[33] = m2l_fma(D[48], m, L[33]);
+      L[34] = m2l_fma(D[49], m, L[34]);
     }
-    { const float m = -__ldg(Ms + 2) * rp;
-      L[0] = fmaf(D[2], m, L[0]);
-      L[1] = fmaf(D[5], m, L[1]);
-      L[2] = fmaf(D[7], m, L[2]);
-      L[3] = fmaf(D[8], m, L[3]);
-      L[4] = fmaf(D[11], m, L[4]);
-      L[5] = fmaf(D[13], m, L[5]);
-      L[6] = fmaf(D[14], m, L[6]);
-      L[7] = fmaf(D[16], m, L[7]);
-      L[8] = fmaf(D[17], m, L[8]);
-      L[9] = fmaf(D[18], m, L[9]);
-      L[10] = fmaf(D[21], m, L[10]);
-      L[11] = fmaf(D[23], m, L[11]);
-      L[12] = fmaf(D[24], m, L[12]);
-      L[13] = fmaf(D[26], m, L[13]);
-      L[14] = fmaf(D[27], m, L[14]);
-      L[15] = fmaf(D[28], m, L[15]);
-      L[16] = fmaf(D[30], m, L[16]);
-      L[17] = fmaf(D[31], m, L[17]);
-      L[18] = fmaf(D[32], m, L[18]);
-      L[19] = fmaf(D[33], m, L[19]);
-      L[20] = fmaf(D[36], m, L[20]);
-      L[21] = fmaf(D[38], m, L[21]);
-      L[22] = fmaf(D[39], m, L[22]);
-      L[23] = fmaf(D[41], m, L[23]);
-      L[24] = fmaf(D[42], m, L[24]);
-      L[25] = fmaf(D[43], m, L[25]);
-      L[26] = fmaf(D[45], m, L[26]);
-      L[27] = fmaf(D[46], m, L[27]);
-      L[28] = fmaf(D[47], m, L[28]);
-      L[29] = fmaf(D[48], m, L[29]);
-      L[30] = fmaf(D[50], m, L[30]);
-      L[31] = fmaf(D[51], m, L[31]);
-      L[32] = fmaf(D[52], m, L[32]);
-      L[33] = fmaf(D[53], m, L[33]);
-      L[34] = fmaf(D[54], m, L[34]);
+    { const T m = -__ldg(Ms + 2) * rp;
+      L[0] = m2l_fma(D[2], m, L[0]);
+      L[1] = m2l_fma(D[5], m, L[1]);
+      L[2] = m2l_fma(D[7], m, L[2]);
+      L[3] = m2l_fma(D[8], m, L[3]);
+      L[4] = m2l_fma(D[11], m, L[4]);
+      L[5] = m2l_fma(D[13], m, L[5]);
+      L[6] = m2l_fma(D[14], m, L[6]);
+      L[7] = m2l_fma(D[16], m, L[7]);
+      L[8] = m2l_fma(D[17], m, L[8]);
+      L[9] = m2l_fma(D[18], m, L[9]);
+      L[10] = m2l_fma(D[21], m, L[10]);
+      L[11] = m2l_fma(D[23], m, L[11]);
+      L[12] = m2l_fma(D[24], m, L[12]);
+      L[13] = m2l_fma(D[26], m, L[13]);
+      L[14] = m2l_fma(D[27], m, L[14]);
+      L[15] = m2l_fma(D[28], m, L[15]);
+      L[16] = m2l_fma(D[30], m, L[16]);
+      L[17] = m2l_fma(D[31], m, L[17]);
+      L[18] = m2l_fma(D[32], m, L[18]);
+      L[19] = m2l_fma(D[33], m, L[19]);
+      L[20] = m2l_fma(D[36], m, L[20]);
+      L[21] = m2l_fma(D[38], m, L[21]);
+      L[22] = m2l_fma(D[39], m, L[22]);
+      L[23] = m2l_fma(D[41], m, L[23]);
+      L[24] = m2l_fma(D[42], m, L[24]);
+      L[25] = m2l_fma(D[43], m, L[25]);
+      L[26] = m2l_fma(D[45], m, L[26]);
+      L[27] = m2l_fma(D[46], m, L[27]);
+      L[28] = m2l_fma(D[47], m, L[28]);
+      L[29] = m2l_fma(D[48], m, L[29]);
+      L[30] = m2l_fma(D[50], m, L[30]);
+      L[31] = m2l_fma(D[51], m, L[31]);
+      L[32] = m2l_fma(D[52], m, L[32]);
+      L[33] = m2l_fma(D[53], m, L[33]);
+      L[34] = m2l_fma(D[54], m, L[34]);
     }
-    { const float m = -__ldg(Ms + 3) * rp;
-      L[0] = fmaf(D[3], m, L[0]);
-      L[1] = fmaf(D[6], m, L[1]);
-      L[2] = fmaf(D[8], m, L[2]);
-      L[3] = fmaf(D[9], m, L[3]);
-      L[4] = fmaf(D[12], m, L[4]);
-      L[5] = fmaf(D[14], m, L[5]);
-      L[6] = fmaf(D[15], m, L[6]);
-      L[7] = fmaf(D[17], m, L[7]);
-      L[8] = fmaf(D[18], m, L[8]);
-      L[9] = fmaf(D[19], m, L[9]);
-      L[10] = fmaf(D[22], m, L[10]);
-      L[11] = fmaf(D[24], m, L[11]);
-      L[12] = fmaf(D[25], m, L[12]);
-      L[13] = fmaf(D[27], m, L[13]);
-      L[14] = fmaf(D[28], m, L[14]);
-      L[15] = fmaf(D[29], m, L[15]);
-      L[16] = fmaf(D[31], m, L[16]);
-      L[17] = fmaf(D[32], m, L[17]);
-      L[18] = fmaf(D[33], m, L[18]);
-      L[19] = fmaf(D[34], m, L[19]);
-      L[20] = fmaf(D[37], m, L[20]);
-      L[21] = fmaf(D[39], m, L[21]);
-      L[22] = fmaf(D[40], m, L[22]);
-      L[23] = fmaf(D[42], m, L[23]);
-      L[24] = fmaf(D[43], m, L[24]);
-      L[25] = fmaf(D[44], m, L[25]);
-      L[26] = fmaf(D[46], m, L[26]);
-      L[27] = fmaf(D[47], m, L[27]);
-      L[28] = fmaf(D[48], m, L[28]);
-      L[29] = fmaf(D[49], m, L[29]);
-      L[30] = fmaf(D[51], m, L[30]);
-      L[31] = fmaf(D[52], m, L[31]);
-      L[32] = fmaf(D[53], m, L[32]);
-      L[33] = fmaf(D[54], m, L[33]);
-      L[34] = fmaf(D[55], m, L[34]);
-    }
-    rp *= rho;
-    { const float m = __ldg(Ms + 4) * rp;
-      L[0] = fmaf(D[4], m, L[0]);
-      L[1] = fmaf(D[10], m, L[1]);
-      L[2] = fmaf(D[11], m, L[2]);
-      L[3] = fmaf(D[12], m, L[3]);
-      L[4] = fmaf(D[20], m, L[4]);
-      L[5] = fmaf(D[21], m, L[5]);
-      L[6] = fmaf(D[22], m, L[6]);
-      L[7] = fmaf(D[23], m, L[7]);
-      L[8] = fmaf(D[24], m, L[8]);
-      L[9] = fmaf(D[25], m, L[9]);
-      L[10] = fmaf(D[35], m, L[10]);
-      L[11] = fmaf(D[36], m, L[11]);
-      L[12] = fmaf(D[37], m, L[12]);
-      L[13] = fmaf(D[38], m, L[13]);
-      L[14] = fmaf(D[39], m, L[14]);
-      L[15] = fmaf(D[40], m, L[15]);
-      L[16] = fmaf(D[41], m, L[16]);
-      L[17] = fmaf(D[42], m, L[17]);
-      L[18] = fmaf(D[43], m, L[18]);
-      L[19] = fmaf(D[44], m, L[19]);
-    }
-    { const float m = __ldg(Ms + 5) * rp;
-      L[0] = fmaf(D[5], m, L[0]);
-      L[1] = fmaf(D[11], m, L[1]);
-      L[2] = fmaf(D[13], m, L[2]);
-      L[3] = fmaf(D[14], m, L[3]);
-      L[4] = fmaf(D[21], m, L[4]);
-      L[5] = fmaf(D[23], m, L[5]);
-      L[6] = fmaf(D[24], m, L[6]);
-      L[7] = fmaf(D[26], m, L[7]);
-      L[8] = fmaf(D[27], m, L[8]);
-      L[9] = fmaf(D[28], m, L[9]);
-      L[10] = fmaf(D[36], m, L[10]);
-      L[11] = fmaf(D[38], m, L[11]);
-      L[12] = fmaf(D[39], m, L[12]);
-      L[13] = fmaf(D[41], m, L[13]);
-      L[14] = fmaf(D[42], m, L[14]);
-      L[15] = fmaf(D[43], m, L[15]);
-      L[16] = fmaf(D[45], m, L[16]);
-      L[17] = fmaf(D[46], m, L[17]);
-      L[18] = fmaf(D[47], m, L[18]);
-      L[19] = fmaf(D[48], m, L[19]);
-    }
-    { const float m = __ldg(Ms + 6) * rp;
-      L[0] = fmaf(D[6], m, L[0]);
-      L[1] = fmaf(D[12], m, L[1]);
-      L[2] = fmaf(D[14], m, L[2]);
-      L[3] = fmaf(D[15], m, L[3]);
-      L[4] = fmaf(D[22], m, L[4]);
-      L[5] = fmaf(D[24], m, L[5]);
-      L[6] = fmaf(D[25], m, L[6]);
-      L[7] = fmaf(D[27], m, L[7]);
-      L[8] = fmaf(D[28], m, L[8]);
-      L[9] = fmaf(D[29], m, L[9]);
-      L[10] = fmaf(D[37], m, L[10]);
-      L[11] = fmaf(D[39], m, L[11]);
-      L[12] = fmaf(D[40], m, L[12]);
-      L[13] = fmaf(D[42], m, L[13]);
-      L[14] = fmaf(D[43], m, L[14]);
-      L[15] = fmaf(D[44], m, L[15]);
-      L[16] = fmaf(D[46], m, L[16]);
-      L[17] = fmaf(D[47], m, L[17]);
-      L[18] = fmaf(D[48], m, L[18]);
-      L[19] = fmaf(D[49], m, L[19]);
-    }
-    { const float m = __ldg(Ms + 7) * rp;
-      L[0] = fmaf(D[7], m, L[0]);
-      L[1] = fmaf(D[13], m, L[1]);
-      L[2] = fmaf(D[16], m, L[2]);
-      L[3] = fmaf(D[17], m, L[3]);
-      L[4] = fmaf(D[23], m, L[4]);
-      L[5] = fmaf(D[26], m, L[5]);
-      L[6] = fmaf(D[27], m, L[6]);
-      L[7] = fmaf(D[30], m, L[7]);
-      L[8] = fmaf(D[31], m, L[8]);
-      L[9] = fmaf(D[32], m, L[9]);
-      L[10] = fmaf(D[38], m, L[10]);
-      L[11] = fmaf(D[41], m, L[11]);
-      L[12] = fmaf(D[42], m, L[12]);
-      L[13] = fmaf(D[45], m, L[13]);
-      L[14] = fmaf(D[46], m, L[14]);
-      L[15] = fmaf(D[47], m, L[15]);
-      L[16] = fmaf(D[50], m, L[16]);
-      L[17] = fmaf(D[51], m, L[17]);
-      L[18] = fmaf(D[52], m, L[18]);
-      L[19] = fmaf(D[53], m, L[19]);
-    }
-    { const float m = __ldg(Ms + 8) * rp;
-      L[0] = fmaf(D[8], m, L[0]);
-      L[1] = fmaf(D[14], m, L[1]);
-      L[2] = fmaf(D[17], m, L[2]);
-      L[3] = fmaf(D[18], m, L[3]);
-      L[4] = fmaf(D[24], m, L[4]);
-      L[5] = fmaf(D[27], m, L[5]);
-      L[6] = fmaf(D[28], m, L[6]);
-      L[7] = fmaf(D[31], m, L[7]);
-      L[8] = fmaf(D[32], m, L[8]);
-      L[9] = fmaf(D[33], m, L[9]);
-      L[10] = fmaf(D[39], m, L[10]);
-      L[11] = fmaf(D[42], m, L[11]);
-      L[12] = fmaf(D[43], m, L[12]);
-      L[13] = fmaf(D[46], m, L[13]);
-      L[14] = fmaf(D[47], m, L[14]);
-      L[15] = fmaf(D[48], m, L[15]);
-      L[16] = fmaf(D[51], m, L[16]);
-      L[17] = fmaf(D[52], m, L[17]);
-      L[18] = fmaf(D[53], m, L[18]);
-      L[19] = fmaf(D[54], m, L[19]);
-    }
-    { const float m = __ldg(Ms + 9) * rp;
-      L[0] = fmaf(D[9], m, L[0]);
-      L[1] = fmaf(D[15], m, L[1]);
-      L[2] = fmaf(D[18], m, L[2]);
-      L[3] = fmaf(D[19], m, L[3]);
-      L[4] = fmaf(D[25], m, L[4]);
-      L[5] = fmaf(D[28], m, L[5]);
-      L[6] = fmaf(D[29], m, L[6]);
-      L[7] = fmaf(D[32], m, L[7]);
-      L[8] = fmaf(D[33], m, L[8]);
-      L[9] = fmaf(D[34], m, L[9]);
-      L[10] = fmaf(D[40], m, L[10]);
-      L[11] = fmaf(D[43], m, L[11]);
-      L[12] = fmaf(D[44], m, L[12]);
-      L[13] = fmaf(D[47], m, L[13]);
-      L[14] = fmaf(D[48], m, L[14]);
-      L[15] = fmaf(D[49], m, L[15]);
-      L[16] = fmaf(D[52], m, L[16]);
-      L[17] = fmaf(D[53], m, L[17]);
-      L[18] = fmaf(D[54], m, L[18]);
-      L[19] = fmaf(D[55], m, L[19]);
+    { const T m = -__ldg(Ms + 3) * rp;
+      L[0] = m2l_fma(D[3], m, L[0]);
+      L[1] = m2l_fma(D[6], m, L[1]);
+      L[2] = m2l_fma(D[8], m, L[2]);
+      L[3] = m2l_fma(D[9], m, L[3]);
+      L[4] = m2l_fma(D[12], m, L[4]);
+      L[5] = m2l_fma(D[14], m, L[5]);
+      L[6] = m2l_fma(D[15], m, L[6]);
+      L[7] = m2l_fma(D[17], m, L[7]);
+      L[8] = m2l_fma(D[18], m, L[8]);
+      L[9] = m2l_fma(D[19], m, L[9]);
+      L[10] = m2l_fma(D[22], m, L[10]);
+      L[11] = m2l_fma(D[24], m, L[11]);
+      L[12] = m2l_fma(D[25], m, L[12]);
+      L[13] = m2l_fma(D[27], m, L[13]);
+      L[14] = m2l_fma(D[28], m, L[14]);
+      L[15] = m2l_fma(D[29], m, L[15]);
+      L[16] = m2l_fma(D[31], m, L[16]);
+      L[17] = m2l_fma(D[32], m, L[17]);
+      L[18] = m2l_fma(D[33], m, L[18]);
+      L[19] = m2l_fma(D[34], m, L[19]);
+      L[20] = m2l_fma(D[37], m, L[20]);
+      L[21] = m2l_fma(D[39], m, L[21]);
+      L[22] = m2l_fma(D[40], m, L[22]);
+      L[23] = m2l_fma(D[42], m, L[23]);
+      L[24] = m2l_fma(D[43], m, L[24]);
+      L[25] = m2l_fma(D[44], m, L[25]);
+      L[26] = m2l_fma(D[46], m, L[26]);
+      L[27] = m2l_fma(D[47], m, L[27]);
+      L[28] = m2l_fma(D[48], m, L[28]);
+      L[29] = m2l_fma(D[49], m, L[29]);
+      L[30] = m2l_fma(D[51], m, L[30]);
+      L[31] = m2l_fma(D[52], m, L[31]);
+      L[32] = m2l_fma(D[53], m, L[32]);
+      L[33] = m2l_fma(D[54], m, L[33]);
+      L[34] = m2l_fma(D[55], m, L[34]);
     }
     rp *= rho;
-    { const float m = -__ldg(Ms + 10) * rp;
-      L[0] = fmaf(D[10], m, L[0]);
-      L[1] = fmaf(D[20], m, L[1]);
-      L[2] = fmaf(D[21], m, L[2]);
-      L[3] = fmaf(D[22], m, L[3]);
-      L[4] = fmaf(D[35], m, L[4]);
-      L[5] = fmaf(D[36], m, L[5]);
-      L[6] = fmaf(D[37], m, L[6]);
-      L[7] = fmaf(D[38], m, L[7]);
-      L[8] = fmaf(D[39], m, L[8]);
-      L[9] = fmaf(D[40], m, L[9]);
+    { const T m = __ldg(Ms + 4) * rp;
+      L[0] = m2l_fma(D[4], m, L[0]);
+      L[1] = m2l_fma(D[10], m, L[1]);
+      L[2] = m2l_fma(D[11], m, L[2]);
+      L[3] = m2l_fma(D[12], m, L[3]);
+      L[4] = m2l_fma(D[20], m, L[4]);
+      L[5] = m2l_fma(D[21], m, L[5]);
+      L[6] = m2l_fma(D[22], m, L[6]);
+      L[7] = m2l_fma(D[23], m, L[7]);
+      L[8] = m2l_fma(D[24], m, L[8]);
+      L[9] = m2l_fma(D[25], m, L[9]);
+      L[10] = m2l_fma(D[35], m, L[10]);
+      L[11] = m2l_fma(D[36], m, L[11]);
+      L[12] = m2l_fma(D[37], m, L[12]);
+      L[13] = m2l_fma(D[38], m, L[13]);
+      L[14] = m2l_fma(D[39], m, L[14]);
+      L[15] = m2l_fma(D[40], m, L[15]);
+      L[16] = m2l_fma(D[41], m, L[16]);
+      L[17] = m2l_fma(D[42], m, L[17]);
+      L[18] = m2l_fma(D[43], m, L[18]);
+      L[19] = m2l_fma(D[44], m, L[19]);
     }
-    { const float m = -__ldg(Ms + 11) * rp;
-      L[0] = fmaf(D[11], m, L[0]);
-      L[1] = fmaf(D[21], m, L[1]);
-      L[2] = fmaf(D[23], m, L[2]);
-      L[3] = fmaf(D[24], m, L[3]);
-      L[4] = fmaf(D[36], m, L[4]);
-      L[5] = fmaf(D[38], m, L[5]);
-      L[6] = fmaf(D[39], m, L[6]);
-      L[7] = fmaf(D[41], m, L[7]);
-      L[8] = fmaf(D[42], m, L[8]);
-      L[9] = fmaf(D[43], m, L[9]);
+    { const T m = __ldg(Ms + 5) * rp;
+      L[0] = m2l_fma(D[5], m, L[0]);
+      L[1] = m2l_fma(D[11], m, L[1]);
+      L[2] = m2l_fma(D[13], m, L[2]);
+      L[3] = m2l_fma(D[14], m, L[3]);
+      L[4] = m2l_fma(D[21], m, L[4]);
+      L[5] = m2l_fma(D[23], m, L[5]);
+      L[6] = m2l_fma(D[24], m, L[6]);
+      L[7] = m2l_fma(D[26], m, L[7]);
+      L[8] = m2l_fma(D[27], m, L[8]);
+      L[9] = m2l_fma(D[28], m, L[9]);
+      L[10] = m2l_fma(D[36], m, L[10]);
+      L[11] = m2l_fma(D[38], m, L[11]);
+      L[12] = m2l_fma(D[39], m, L[12]);
+      L[13] = m2l_fma(D[41], m, L[13]);
+      L[14] = m2l_fma(D[42], m, L[14]);
+      L[15] = m2l_fma(D[43], m, L[15]);
+      L[16] = m2l_fma(D[45], m, L[16]);
+      L[17] = m2l_fma(D[46], m, L[17]);
+      L[18] = m2l_fma(D[47], m, L[18]);
+      L[19] = m2l_fma(D[48], m, L[19]);
     }
-    { const float m = -__ldg(Ms + 12) * rp;
-      L[0] = fmaf(D[12], m, L[0]);
-      L[1] = fmaf(D[22], m, L[1]);
-      L[2] = fmaf(D[24], m, L[2]);
-      L[3] = fmaf(D[25], m, L[3]);
-      L[4] = fmaf(D[37], m, L[4]);
-      L[5] = fmaf(D[39], m, L[5]);
-      L[6] = fmaf(D[40], m, L[6]);
-      L[7] = fmaf(D[42], m, L[7]);
-      L[8] = fmaf(D[43], m, L[8]);
-      L[9] = fmaf(D[44], m, L[9]);
+    { const T m = __ldg(Ms + 6) * rp;
+      L[0] = m2l_fma(D[6], m, L[0]);
+      L[1] = m2l_fma(D[12], m, L[1]);
+      L[2] = m2l_fma(D[14], m, L[2]);
+      L[3] = m2l_fma(D[15], m, L[3]);
+      L[4] = m2l_fma(D[22], m, L[4]);
+      L[5] = m2l_fma(D[24], m, L[5]);
+      L[6] = m2l_fma(D[25], m, L[6]);
+      L[7] = m2l_fma(D[27], m, L[7]);
+      L[8] = m2l_fma(D[28], m, L[8]);
+      L[9] = m2l_fma(D[29], m, L[9]);
+      L[10] = m2l_fma(D[37], m, L[10]);
+      L[11] = m2l_fma(D[39], m, L[11]);
+      L[12] = m2l_fma(D[40], m, L[12]);
+      L[13] = m2l_fma(D[42], m, L[13]);
+      L[14] = m2l_fma(D[43], m, L[14]);
+      L[15] = m2l_fma(D[44], m, L[15]);
+      L[16] = m2l_fma(D[46], m, L[16]);
+      L[17] = m2l_fma(D[47], m, L[17]);
+      L[18] = m2l_fma(D[48], m, L[18]);
+      L[19] = m2l_fma(D[49], m, L[19]);
     }
-    { const float m = -__ldg(Ms + 13) * rp;
-      L[0] = fmaf(D[13], m, L[0]);
-      L[1] = fmaf(D[23], m, L[1]);
-      L[2] = fmaf(D[26], m, L[2]);
-      L[3] = fmaf(D[27], m, L[3]);
-      L[4] = fmaf(D[38], m, L[4]);
-      L[5] = fmaf(D[41], m, L[5]);
-      L[6] = fmaf(D[42], m, L[6]);
-      L[7] = fmaf(D[45], m, L[7]);
-      L[8] = fmaf(D[46], m, L[8]);
-      L[9] = fmaf(D[47], m, L[9]);
+    { const T m = __ldg(Ms + 7) * rp;
+      L[0] = m2l_fma(D[7], m, L[0]);
+      L[1] = m2l_fma(D[13], m, L[1]);
+      L[2] = m2l_fma(D[16], m, L[2]);
+      L[3] = m2l_fma(D[17], m, L[3]);
+      L[4] = m2l_fma(D[23], m, L[4]);
+      L[5] = m2l_fma(D[26], m, L[5]);
+      L[6] = m2l_fma(D[27], m, L[6]);
+      L[7] = m2l_fma(D[30], m, L[7]);
+      L[8] = m2l_fma(D[31], m, L[8]);
+      L[9] = m2l_fma(D[32], m, L[9]);
+      L[10] = m2l_fma(D[38], m, L[10]);
+      L[11] = m2l_fma(D[41], m, L[11]);
+      L[12] = m2l_fma(D[42], m, L[12]);
+      L[13] = m2l_fma(D[45], m, L[13]);
+      L[14] = m2l_fma(D[46], m, L[14]);
+      L[15] = m2l_fma(D[47], m, L[15]);
+      L[16] = m2l_fma(D[50], m, L[16]);
+      L[17] = m2l_fma(D[51], m, L[17]);
+      L[18] = m2l_fma(D[52], m, L[18]);
+      L[19] = m2l_fma(D[53], m, L[19]);
     }
-    { const float m = -__ldg(Ms + 14) * rp;
-      L[0] = fmaf(D[14], m, L[0]);
-      L[1] = fmaf(D[24], m, L[1]);
-      L[2] = fmaf(D[27], m, L[2]);
-      L[3] = fmaf(D[28], m, L[3]);
-      L[4] = fmaf(D[39], m, L[4]);
-      L[5] = fmaf(D[42], m, L[5]);
-      L[6] = fmaf(D[43], m, L[6]);
-      L[7] = fmaf(D[46], m, L[7]);
-      L[8] = fmaf(D[47], m, L[8]);
-      L[9] = fmaf(D[48], m, L[9]);
+    { const T m = __ldg(Ms + 8) * rp;
+      L[0] = m2l_fma(D[8], m, L[0]);
+      L[1] = m2l_fma(D[14], m, L[1]);
+      L[2] = m2l_fma(D[17], m, L[2]);
+      L[3] = m2l_fma(D[18], m, L[3]);
+      L[4] = m2l_fma(D[24], m, L[4]);
+      L[5] = m2l_fma(D[27], m, L[5]);
+      L[6] = m2l_fma(D[28], m, L[6]);
+      L[7] = m2l_fma(D[31], m, L[7]);
+      L[8] = m2l_fma(D[32], m, L[8]);
+      L[9] = m2l_fma(D[33], m, L[9]);
+      L[10] = m2l_fma(D[39], m, L[10]);
+      L[11] = m2l_fma(D[42], m, L[11]);
+      L[12] = m2l_fma(D[43], m, L[12]);
+      L[13] = m2l_fma(D[46], m, L[13]);
+      L[14] = m2l_fma(D[47], m, L[14]);
+      L[15] = m2l_fma(D[48], m, L[15]);
+      L[16] = m2l_fma(D[51], m, L[16]);
+      L[17] = m2l_fma(D[52], m, L[17]);
+      L[18] = m2l_fma(D[53], m, L[18]);
+      L[19] = m2l_fma(D[54], m, L[19]);
     }
-    { const float m = -__ldg(Ms + 15) * rp;
-      L[0] = fmaf(D[15], m, L[0]);
-      L[1] = fmaf(D[25], m, L[1]);
-      L[2] = fmaf(D[28], m, L[2]);
-      L[3] = fmaf(D[29], m, L[3]);
-      L[4] = fmaf(D[40], m, L[4]);
-      L[5] = fmaf(D[43], m, L[5]);
-      L[6] = fmaf(D[44], m, L[6]);
-      L[7] = fmaf(D[47], m, L[7]);
-      L[8] = fmaf(D[48], m, L[8]);
-      L[9] = fmaf(D[49], m, L[9]);
-    }
-    { const float m = -__ldg(Ms + 16) * rp;
-      L[0] = fmaf(D[16], m, L[0]);
-      L[1] = fmaf(D[26], m, L[1]);
-      L[2] = fmaf(D[30], m, L[2]);
-      L[3] = fmaf(D[31], m, L[3]);
-      L[4] = fmaf(D[41], m, L[4]);
-      L[5] = fmaf(D[45], m, L[5]);
-      L[6] = fmaf(D[46], m, L[6]);
-      L[7] = fmaf(D[50], m, L[7]);
-      L[8] = fmaf(D[51], m, L[8]);
-      L[9] = fmaf(D[52], m, L[9]);
-    }
-    { const float m = -__ldg(Ms + 17) * rp;
-      L[0] = fmaf(D[17], m, L[0]);
-      L[1] = fmaf(D[27], m, L[1]);
-      L[2] = fmaf(D[31], m, L[2]);
-      L[3] = fmaf(D[32], m, L[3]);
-      L[4] = fmaf(D[42], m, L[4]);
-      L[5] = fmaf(D[46], m, L[5]);
-      L[6] = fmaf(D[47], m, L[6]);
-      L[7] = fmaf(D[51], m, L[7]);
-      L[8] = fmaf(D[52], m, L[8]);
-      L[9] = fmaf(D[53], m, L[9]);
-    }
-    { const float m = -__ldg(Ms + 18) * rp;
-      L[0] = fmaf(D[18], m, L[0]);
-      L[1] = fmaf(D[28], m, L[1]);
-      L[2] = fmaf(D[32], m, L[2]);
-      L[3] = fmaf(D[33], m, L[3]);
-      L[4] = fmaf(D[43], m, L[4]);
-      L[5] = fmaf(D[47], m, L[5]);
-      L[6] = fmaf(D[48], m, L[6]);
-      L[7] = fmaf(D[52], m, L[7]);
-      L[8] = fmaf(D[53], m, L[8]);
-      L[9] = fmaf(D[54], m, L[9]);
-    }
-    { const float m = -__ldg(Ms + 19) * rp;
-      L[0] = fmaf(D[19], m, L[0]);
-      L[1] = fmaf(D[29], m, L[1]);
-      L[2] = fmaf(D[33], m, L[2]);
-      L[3] = fmaf(D[34], m, L[3]);
-      L[4] = fmaf(D[44], m, L[4]);
-      L[5] = fmaf(D[48], m, L[5]);
-      L[6] = fmaf(D[49], m, L[6]);
-      L[7] = fmaf(D[53], m, L[7]);
-      L[8] = fmaf(D[54], m, L[8]);
-      L[9] = fmaf(D[55], m, L[9]);
-    }
-    rp *= rho;
-    { const float m = __ldg(Ms + 20) * rp;
-      L[0] = fmaf(D[20], m, L[0]);
-      L[1] = fmaf(D[35], m, L[1]);
-      L[2] = fmaf(D[36], m, L[2]);
-      L[3] = fmaf(D[37], m, L[3]);
-    }
-    { const float m = __ldg(Ms + 21) * rp;
-      L[0] = fmaf(D[21], m, L[0]);
-      L[1] = fmaf(D[36], m, L[1]);
-      L[2] = fmaf(D[38], m, L[2]);
-      L[3] = fmaf(D[39], m, L[3]);
-    }
-    { const float m = __ldg(Ms + 22) * rp;
-      L[0] = fmaf(D[22], m, L[0]);
-      L[1] = fmaf(D[37], m, L[1]);
-      L[2] = fmaf(D[39], m, L[2]);
-      L[3] = fmaf(D[40], m, L[3]);
-    }
-    { const float m = __ldg(Ms + 23) * rp;
-      L[0] = fmaf(D[23], m, L[0]);
-      L[1] = fmaf(D[38], m, L[1]);
-      L[2] = fmaf(D[41], m, L[2]);
-      L[3] = fmaf(D[42], m, L[3]);
-    }
-    { const float m = __ldg(Ms + 24) * rp;
-      L[0] = fmaf(D[24], m, L[0]);
-      L[1] = fmaf(D[39], m, L[1]);
-      L[2] = fmaf(D[42], m, L[2]);
-      L[3] = fmaf(D[43], m, L[3]);
-    }
-    { const float m = __ldg(Ms + 25) * rp;
-      L[0] = fmaf(D[25], m, L[0]);
-      L[1] = fmaf(D[40], m, L[1]);
-      L[2] = fmaf(D[43], m, L[2]);
-      L[3] = fmaf(D[44], m, L[3]);
-    }
-    { const float m = __ldg(Ms + 26) * rp;
-      L[0] = fmaf(D[26], m, L[0]);
-      L[1] = fmaf(D[41], m, L[1]);
-      L[2] = fmaf(D[45], m, L[2]);
-      L[3] = fmaf(D[46], m, L[3]);
-    }
-    { const float m = __ldg(Ms + 27) * rp;
-      L[0] = fmaf(D[27], m, L[0]);
-      L[1] = fmaf(D[42], m, L[1]);
-      L[2] = fmaf(D[46], m, L[2]);
-      L[3] = fmaf(D[47], m, L[3]);
-    }
-    { const float m = __ldg(Ms + 28) * rp;
-      L[0] = fmaf(D[28], m, L[0]);
-      L[1] = fmaf(D[43], m, L[1]);
-      L[2] = fmaf(D[47], m, L[2]);
-      L[3] = fmaf(D[48], m, L[3]);
-    }
-    { const float m = __ldg(Ms + 29) * rp;
-      L[0] = fmaf(D[29], m, L[0]);
-      L[1] = fmaf(D[44], m, L[1]);
-      L[2] = fmaf(D[48], m, L[2]);
-      L[3] = fmaf(D[49], m, L[3]);
-    }
-    { const float m = __ldg(Ms + 30) * rp;
-      L[0] = fmaf(D[30], m, L[0]);
-      L[1] = fmaf(D[45], m, L[1]);
-      L[2] = fmaf(D[50], m, L[2]);
-      L[3] = fmaf(D[51], m, L[3]);
-    }
-    { const float m = __ldg(Ms + 31) * rp;
-      L[0] = fmaf(D[31], m, L[0]);
-      L[1] = fmaf(D[46], m, L[1]);
-      L[2] = fmaf(D[51], m, L[2]);
-      L[3] = fmaf(D[52], m, L[3]);
-    }
-    { const float m = __ldg(Ms + 32) * rp;
-      L[0] = fmaf(D[32], m, L[0]);
-      L[1] = fmaf(D[47], m, L[1]);
-      L[2] = fmaf(D[52], m, L[2]);
-      L[3] = fmaf(D[53], m, L[3]);
-    }
-    { const float m = __ldg(Ms + 33) * rp;
-      L[0] = fmaf(D[33], m, L[0]);
-      L[1] = fmaf(D[48], m, L[1]);
-      L[2] = fmaf(D[53], m, L[2]);
-      L[3] = fmaf(D[54], m, L[3]);
-    }
-    { const float m = __ldg(Ms + 34) * rp;
-      L[0] = fmaf(D[34], m, L[0]);
-      L[1] = fmaf(D[49], m, L[1]);
-      L[2] = fmaf(D[54], m, L[2]);
-      L[3] = fmaf(D[55], m, L[3]);
+    { const T m = __ldg(Ms + 9) * rp;
+      L[0] = m2l_fma(D[9], m, L[0]);
+      L[1] = m2l_fma(D[15], m, L[1]);
+      L[2] = m2l_fma(D[18], m, L[2]);
+      L[3] = m2l_fma(D[19], m, L[3]);
+      L[4] = m2l_fma(D[25], m, L[4]);
+      L[5] = m2l_fma(D[28], m, L[5]);
+      L[6] = m2l_fma(D[29], m, L[6]);
+      L[7] = m2l_fma(D[32], m, L[7]);
+      L[8] = m2l_fma(D[33], m, L[8]);
+      L[9] = m2l_fma(D[34], m, L[9]);
+      L[10] = m2l_fma(D[40], m, L[10]);
+      L[11] = m2l_fma(D[43], m, L[11]);
+      L[12] = m2l_fma(D[44], m, L[12]);
+      L[13] = m2l_fma(D[47], m, L[13]);
+      L[14] = m2l_fma(D[48], m, L[14]);
+      L[15] = m2l_fma(D[49], m, L[15]);
+      L[16] = m2l_fma(D[52], m, L[16]);
+      L[17] = m2l_fma(D[53], m, L[17]);
+      L[18] = m2l_fma(D[54], m, L[18]);
+      L[19] = m2l_fma(D[55], m, L[19]);
     }
     rp *= rho;
-    { const float m = -__ldg(Ms + 35) * rp;
-      L[0] = fmaf(D[35], m, L[0]);
+    { const T m = -__ldg(Ms + 10) * rp;
+      L[0] = m2l_fma(D[10], m, L[0]);
+      L[1] = m2l_fma(D[20], m, L[1]);
+      L[2] = m2l_fma(D[21], m, L[2]);
+      L[3] = m2l_fma(D[22], m, L[3]);
+      L[4] = m2l_fma(D[35], m, L[4]);
+      L[5] = m2l_fma(D[36], m, L[5]);
+      L[6] = m2l_fma(D[37], m, L[6]);
+      L[7] = m2l_fma(D[38], m, L[7]);
+      L[8] = m2l_fma(D[39], m, L[8]);
+      L[9] = m2l_fma(D[40], m, L[9]);
     }
-    { const float m = -__ldg(Ms + 36) * rp;
-      L[0] = fmaf(D[36], m, L[0]);
+    { const T m = -__ldg(Ms + 11) * rp;
+      L[0] = m2l_fma(D[11], m, L[0]);
+      L[1] = m2l_fma(D[21], m, L[1]);
+      L[2] = m2l_fma(D[23], m, L[2]);
+      L[3] = m2l_fma(D[24], m, L[3]);
+      L[4] = m2l_fma(D[36], m, L[4]);
+      L[5] = m2l_fma(D[38], m, L[5]);
+      L[6] = m2l_fma(D[39], m, L[6]);
+      L[7] = m2l_fma(D[41], m, L[7]);
+      L[8] = m2l_fma(D[42], m, L[8]);
+      L[9] = m2l_fma(D[43], m, L[9]);
     }
-    { const float m = -__ldg(Ms + 37) * rp;
-      L[0] = fmaf(D[37], m, L[0]);
+    { const T m = -__ldg(Ms + 12) * rp;
+      L[0] = m2l_fma(D[12], m, L[0]);
+      L[1] = m2l_fma(D[22], m, L[1]);
+      L[2] = m2l_fma(D[24], m, L[2]);
+      L[3] = m2l_fma(D[25], m, L[3]);
+      L[4] = m2l_fma(D[37], m, L[4]);
+      L[5] = m2l_fma(D[39], m, L[5]);
+      L[6] = m2l_fma(D[40], m, L[6]);
+      L[7] = m2l_fma(D[42], m, L[7]);
+      L[8] = m2l_fma(D[43], m, L[8]);
+      L[9] = m2l_fma(D[44], m, L[9]);
     }
-    { const float m = -__ldg(Ms + 38) * rp;
-      L[0] = fmaf(D[38], m, L[0]);
+    { const T m = -__ldg(Ms + 13) * rp;
+      L[0] = m2l_fma(D[13], m, L[0]);
+      L[1] = m2l_fma(D[23], m, L[1]);
+      L[2] = m2l_fma(D[26], m, L[2]);
+      L[3] = m2l_fma(D[27], m, L[3]);
+      L[4] = m2l_fma(D[38], m, L[4]);
+      L[5] = m2l_fma(D[41], m, L[5]);
+      L[6] = m2l_fma(D[42], m, L[6]);
+      L[7] = m2l_fma(D[45], m, L[7]);
+      L[8] = m2l_fma(D[46], m, L[8]);
+      L[9] = m2l_fma(D[47], m, L[9]);
     }
-    { const float m = -__ldg(Ms + 39) * rp;
-      L[0] = fmaf(D[39], m, L[0]);
+    { const T m = -__ldg(Ms + 14) * rp;
+      L[0] = m2l_fma(D[14], m, L[0]);
+      L[1] = m2l_fma(D[24], m, L[1]);
+      L[2] = m2l_fma(D[27], m, L[2]);
+      L[3] = m2l_fma(D[28], m, L[3]);
+      L[4] = m2l_fma(D[39], m, L[4]);
+      L[5] = m2l_fma(D[42], m, L[5]);
+      L[6] = m2l_fma(D[43], m, L[6]);
+      L[7] = m2l_fma(D[46], m, L[7]);
+      L[8] = m2l_fma(D[47], m, L[8]);
+      L[9] = m2l_fma(D[48], m, L[9]);
     }
-    { const float m = -__ldg(Ms + 40) * rp;
-      L[0] = fmaf(D[40], m, L[0]);
+    { const T m = -__ldg(Ms + 15) * rp;
+      L[0] = m2l_fma(D[15], m, L[0]);
+      L[1] = m2l_fma(D[25], m, L[1]);
+      L[2] = m2l_fma(D[28], m, L[2]);
+      L[3] = m2l_fma(D[29], m, L[3]);
+      L[4] = m2l_fma(D[40], m, L[4]);
+      L[5] = m2l_fma(D[43], m, L[5]);
+      L[6] = m2l_fma(D[44], m, L[6]);
+      L[7] = m2l_fma(D[47], m, L[7]);
+      L[8] = m2l_fma(D[48], m, L[8]);
+      L[9] = m2l_fma(D[49], m, L[9]);
     }
-    { const float m = -__ldg(Ms + 41) * rp;
-      L[0] = fmaf(D[41], m, L[0]);
+    { const T m = -__ldg(Ms + 16) * rp;
+      L[0] = m2l_fma(D[16], m, L[0]);
+      L[1] = m2l_fma(D[26], m, L[1]);
+      L[2] = m2l_fma(D[30], m, L[2]);
+      L[3] = m2l_fma(D[31], m, L[3]);
+      L[4] = m2l_fma(D[41], m, L[4]);
+      L[5] = m2l_fma(D[45], m, L[5]);
+      L[6] = m2l_fma(D[46], m, L[6]);
+      L[7] = m2l_fma(D[50], m, L[7]);
+      L[8] = m2l_fma(D[51], m, L[8]);
+      L[9] = m2l_fma(D[52], m, L[9]);
     }
-    { const float m = -__ldg(Ms + 42) * rp;
-      L[0] = fmaf(D[42], m, L[0]);
+    { const T m = -__ldg(Ms + 17) * rp;
+      L[0] = m2l_fma(D[17], m, L[0]);
+      L[1] = m2l_fma(D[27], m, L[1]);
+      L[2] = m2l_fma(D[31], m, L[2]);
+      L[3] = m2l_fma(D[32], m, L[3]);
+      L[4] = m2l_fma(D[42], m, L[4]);
+      L[5] = m2l_fma(D[46], m, L[5]);
+      L[6] = m2l_fma(D[47], m, L[6]);
+      L[7] = m2l_fma(D[51], m, L[7]);
+      L[8] = m2l_fma(D[52], m, L[8]);
+      L[9] = m2l_fma(D[53], m, L[9]);
     }
-    { const float m = -__ldg(Ms + 43) * rp;
-      L[0] = fmaf(D[43], m, L[0]);
+    { const T m = -__ldg(Ms + 18) * rp;
+      L[0] = m2l_fma(D[18], m, L[0]);
+      L[1] = m2l_fma(D[28], m, L[1]);
+      L[2] = m2l_fma(D[32], m, L[2]);
+      L[3] = m2l_fma(D[33], m, L[3]);
+      L[4] = m2l_fma(D[43], m, L[4]);
+      L[5] = m2l_fma(D[47], m, L[5]);
+      L[6] = m2l_fma(D[48], m, L[6]);
+      L[7] = m2l_fma(D[52], m, L[7]);
+      L[8] = m2l_fma(D[53], m, L[8]);
+      L[9] = m2l_fma(D[54], m, L[9]);
     }
-    { const float m = -__ldg(Ms + 44) * rp;
-      L[0] = fmaf(D[44], m, L[0]);
+    { const T m = -__ldg(Ms + 19) * rp;
+      L[0] = m2l_fma(D[19], m, L[0]);
+      L[1] = m2l_fma(D[29], m, L[1]);
+      L[2] = m2l_fma(D[33], m, L[2]);
+      L[3] = m2l_fma(D[34], m, L[3]);
+      L[4] = m2l_fma(D[44], m, L[4]);
+      L[5] = m2l_fma(D[48], m, L[5]);
+      L[6] = m2l_fma(D[49], m, L[6]);
+      L[7] = m2l_fma(D[53], m, L[7]);
+      L[8] = m2l_fma(D[54], m, L[8]);
+      L[9] = m2l_fma(D[55], m, L[9]);
     }
-    { const float m = -__ldg(Ms + 45) * rp;
-      L[0] = fmaf(D[45], m, L[0]);
+    rp *= rho;
+    { const T m = __ldg(Ms + 20) * rp;
+      L[0] = m2l_fma(D[20], m, L[0]);
+      L[1] = m2l_fma(D[35], m, L[1]);
+      L[2] = m2l_fma(D[36], m, L[2]);
+      L[3] = m2l_fma(D[37], m, L[3]);
     }
-    { const float m = -__ldg(Ms + 46) * rp;
-      L[0] = fmaf(D[46], m, L[0]);
+    { const T m = __ldg(Ms + 21) * rp;
+      L[0] = m2l_fma(D[21], m, L[0]);
+      L[1] = m2l_fma(D[36], m, L[1]);
+      L[2] = m2l_fma(D[38], m, L[2]);
+      L[3] = m2l_fma(D[39], m, L[3]);
     }
-    { const float m = -__ldg(Ms + 47) * rp;
-      L[0] = fmaf(D[47], m, L[0]);
+    { const T m = __ldg(Ms + 22) * rp;
+      L[0] = m2l_fma(D[22], m, L[0]);
+      L[1] = m2l_fma(D[37], m, L[1]);
+      L[2] = m2l_fma(D[39], m, L[2]);
+      L[3] = m2l_fma(D[40], m, L[3]);
     }
-    { const float m = -__ldg(Ms + 48) * rp;
-      L[0] = fmaf(D[48], m, L[0]);
+    { const T m = __ldg(Ms + 23) * rp;
+      L[0] = m2l_fma(D[23], m, L[0]);
+      L[1] = m2l_fma(D[38], m, L[1]);
+      L[2] = m2l_fma(D[41], m, L[2]);
+      L[3] = m2l_fma(D[42], m, L[3]);
     }
-    { const float m = -__ldg(Ms + 49) * rp;
-      L[0] = fmaf(D[49], m, L[0]);
+    { const T m = __ldg(Ms + 24) * rp;
+      L[0] = m2l_fma(D[24], m, L[0]);
+      L[1] = m2l_fma(D[39], m, L[1]);
+      L[2] = m2l_fma(D[42], m, L[2]);
+      L[3] = m2l_fma(D[43], m, L[3]);
     }
-    { const float m = -__ldg(Ms + 50) * rp;
-      L[0] = fmaf(D[50], m, L[0]);
+    { const T m = __ldg(Ms + 25) * rp;
+      L[0] = m2l_fma(D[25], m, L[0]);
+      L[1] = m2l_fma(D[40], m, L[1]);
+      L[2] = m2l_fma(D[43], m, L[2]);
+      L[3] = m2l_fma(D[44], m, L[3]);
     }
-    { const float m = -__ldg(Ms + 51) * rp;
-      L[0] = fmaf(D[51], m, L[0]);
+    { const T m = __ldg(Ms + 26) * rp;
+      L[0] = m2l_fma(D[26], m, L[0]);
+      L[1] = m2l_fma(D[41], m, L[1]);
+      L[2] = m2l_fma(D[45], m, L[2]);
+      L[3] = m2l_fma(D[46], m, L[3]);
     }
-    { const float m = -__ldg(Ms + 52) * rp;
-      L[0] = fmaf(D[52], m, L[0]);
+    { const T m = __ldg(Ms + 27) * rp;
+      L[0] = m2l_fma(D[27], m, L[0]);
+      L[1] = m2l_fma(D[42], m, L[1]);
+      L[2] = m2l_fma(D[46], m, L[2]);
+      L[3] = m2l_fma(D[47], m, L[3]);
     }
-    { const float m = -__ldg(Ms + 53) * rp;
-      L[0] = fmaf(D[53], m, L[0]);
+    { const T m = __ldg(Ms + 28) * rp;
+      L[0] = m2l_fma(D[28], m, L[0]);
+      L[1] = m2l_fma(D[43], m, L[1]);
+      L[2] = m2l_fma(D[47], m, L[2]);
+      L[3] = m2l_fma(D[48], m, L[3]);
     }
-    { const float m = -__ldg(Ms + 54) * rp;
-      L[0] = fmaf(D[54], m, L[0]);
+    { const T m = __ldg(Ms + 29) * rp;
+      L[0] = m2l_fma(D[29], m, L[0]);
+      L[1] = m2l_fma(D[44], m, L[1]);
+      L[2] = m2l_fma(D[48], m, L[2]);
+      L[3] = m2l_fma(D[49], m, L[3]);
     }
-    { const float m = -__ldg(Ms + 55) * rp;
-      L[0] = fmaf(D[55], m, L[0]);
+    { const T m = __ldg(Ms + 30) * rp;
+      L[0] = m2l_fma(D[30], m, L[0]);
+      L[1] = m2l_fma(D[45], m, L[1]);
+      L[2] = m2l_fma(D[50], m, L[2]);
+      L[3] = m2l_fma(D[51], m, L[3]);
+    }
+    { const T m = __ldg(Ms + 31) * rp;
+      L[0] = m2l_fma(D[31], m, L[0]);
+      L[1] = m2l_fma(D[46], m, L[1]);
+      L[2] = m2l_fma(D[51], m, L[2]);
+      L[3] = m2l_fma(D[52], m, L[3]);
+    }
+    { const T m = __ldg(Ms + 32) * rp;
+      L[0] = m2l_fma(D[32], m, L[0]);
+      L[1] = m2l_fma(D[47], m, L[1]);
+      L[2] = m2l_fma(D[52], m, L[2]);
+      L[3] = m2l_fma(D[53], m, L[3]);
+    }
+    { const T m = __ldg(Ms + 33) * rp;
+      L[0] = m2l_fma(D[33], m, L[0]);
+      L[1] = m2l_fma(D[48], m, L[1]);
+      L[2] = m2l_fma(D[53], m, L[2]);
+      L[3] = m2l_fma(D[54], m, L[3]);
+    }
+    { const T m = __ldg(Ms + 34) * rp;
+      L[0] = m2l_fma(D[34], m, L[0]);
+      L[1] = m2l_fma(D[49], m, L[1]);
+      L[2] = m2l_fma(D[54], m, L[2]);
+      L[3] = m2l_fma(D[55], m, L[3]);
+    }
+    rp *= rho;
+    { const T m = -__ldg(Ms + 35) * rp;
+      L[0] = m2l_fma(D[35], m, L[0]);
+    }
+    { const T m = -__ldg(Ms + 36) * rp;
+      L[0] = m2l_fma(D[36], m, L[0]);
+    }
+    { const T m = -__ldg(Ms + 37) * rp;
+      L[0] = m2l_fma(D[37], m, L[0]);
+    }
+    { const T m = -__ldg(Ms + 38) * rp;
+      L[0] = m2l_fma(D[38], m, L[0]);
+    }
+    { const T m = -__ldg(Ms + 39) * rp;
+      L[0] = m2l_fma(D[39], m, L[0]);
+    }
+    { const T m = -__ldg(Ms + 40) * rp;
+      L[0] = m2l_fma(D[40], m, L[0]);
+    }
+    { const T m = -__ldg(Ms + 41) * rp;
+      L[0] = m2l_fma(D[41], m, L[0]);
+    }
+    { const T m = -__ldg(Ms + 42) * rp;
+      L[0] = m2l_fma(D[42], m, L[0]);
+    }
+    { const T m = -__ldg(Ms + 43) * rp;
+      L[0] = m2l_fma(D[43], m, L[0]);
+    }
+    { const T m = -__ldg(Ms + 44) * rp;
+      L[0] = m2l_fma(D[44], m, L[0]);
+    }
+    { const T m = -__ldg(Ms + 45) * rp;
+      L[0] = m2l_fma(D[45], m, L[0]);
+    }
+    { const T m = -__ldg(Ms + 46) * rp;
+      L[0] = m2l_fma(D[46], m, L[0]);
+    }
+    { const T m = -__ldg(Ms + 47) * rp;
+      L[0] = m2l_fma(D[47], m, L[0]);
+    }
+    { const T m = -__ldg(Ms + 48) * rp;
+      L[0] = m2l_fma(D[48], m, L[0]);
+    }
+    { const T m = -__ldg(Ms + 49) * rp;
+      L[0] = m2l_fma(D[49], m, L[0]);
+    }
+    { const T m = -__ldg(Ms + 50) * rp;
+      L[0] = m2l_fma(D[50], m, L[0]);
+    }
+    { const T m = -__ldg(Ms + 51) * rp;
+      L[0] = m2l_fma(D[51], m, L[0]);
+    }
+    { const T m = -__ldg(Ms + 52) * rp;
+      L[0] = m2l_fma(D[52], m, L[0]);
+    }
+    { const T m = -__ldg(Ms + 53) * rp;
+      L[0] = m2l_fma(D[53], m, L[0]);
+    }
+    { const T m = -__ldg(Ms + 54) * rp;
+      L[0] = m2l_fma(D[54], m, L[0]);
+    }
+    { const T m = -__ldg(Ms + 55) * rp;
+      L[0] = m2l_fma(D[55], m, L[0]);
     }
 }
 
-__device__ __forceinline__ void m2l_side_b_5(const float (&D)[56], const float *__restrict__ Ms, float (&L)[56])
+template <class T> __device__ __forceinline__ void m2l_side_b_5(const T (&D)[56], const T *__restrict__ Ms, T (&L)[56])
 {
-    { const float m = __ldg(Ms + 0);
+    { const T m = __ldg(Ms + 0);
       L[0] = D[0] * m;
       L[1] = -D[1] * m;
       L[2] = -D[2] * m;
@@ -2771,529 +2777,529 @@ __device__ __forceinline__ void m2l_side_b_5(const float (&D)[56], const float *
       L[54] = -D[54] * m;
       L[55] = -D[55] * m;
     }
-    { const float m = __ldg(Ms + 1);
-      L[0] = fmaf(D[1], m, L[0]);
-      L[1] = fmaf(-D[4], m, L[1]);
-      L[2] = fmaf(-D[5], m, L[2]);
-      L[3] = fmaf(-D[6], m, L[3]);
-      L[4] = fmaf(D[10], m, L[4]);
-      L[5] = fmaf(D[11], m, L[5]);
-      L[6] = fmaf(D[12], m, L[6]);
-      L[7] = fmaf(D[13], m, L[7]);
-      L[8] = fmaf(D[14], m, L[8]);
-      L[9] = fmaf(D[15], m, L[9]);
-      L[10] = fmaf(-D[20], m, L[10]);
-      L[11] = fmaf(-D[21], m, L[11]);
-      L[12] = fmaf(-D[22], m, L[12]);
-      L[13] = fmaf(-D[23], m, L[13]);
-      L[14] = fmaf(-D[24], m, L[14]);
-      L[15] = fmaf(-D[25], m, L[15]);
-      L[16] = fmaf(-D[26], m, L[16]);
-      L[17] = fmaf(-D[27], m, L[17]);
-      L[18] = fmaf(-D[28], m, L[18]);
-      L[19] = fmaf(-D[29], m, L[19]);
-      L[20] = fmaf(D[35], m, L[20]);
-      L[21] = fmaf(D[36], m, L[21]);
-      L[22] = fmaf(D[37], m, L[22]);
-      L[23] = fmaf(D[38], m, L[23]);
-      L[24] = fmaf(D[39], m, L[24]);
-      L[25] = fmaf(D[40], m, L[25]);
-      L[26] = fmaf(D[41], m, L[26]);
-      L[27] = fmaf(D[42], m, L[27]);
-      L[28] = fmaf(D[43], m, L[28]);
-      L[29] = fmaf(D[44], m, L[29]);
-      L[30] = fmaf(D[45], m, L[30]);
-      L[31] = fmaf(D[46], m, L[31]);
-      L[32] = fmaf(D[47], m, L[32]);
-      L[33] = fmaf(D[48], m, L[33]);
-      L[34] = fmaf(D[49], m, L[34]);
+    { const T m = __ldg(Ms + 1);
+      L[0] = m2l_fma(D[1], m, L[0]);
+      L[1] = m2l_fma(-D[4], m, L[1]);
+      L[2] = m2l_fma(-D[5], m, L[2]);
+      L[3] = m2l_fma(-D[6], m, L[3]);
+      L[4] = m2l_fma(D[10], m, L[4]);
+      L[5] = m2l_fma(D[11], m, L[5]);
+      L[6] = m2l_fma(D[12], m, L[6]);
+      L[7] = m2l_fma(D[13], m, L[7]);
+      L[8] = m2l_fma(D[14], m, L[8]);
+      L[9] = m2l_fma(D[15], m, L[9]);
+      L[10] = m2l_fma(-D[20], m, L[10]);
+      L[11] = m2l_fma(-D[21], m, L[11]);
+      L[12] = m2l_fma(-D[22], m, L[12]);
+      L[13] = m2l_fma(-D[23], m, L[13]);
+      L[14] = m2l_fma(-D[24], m, L[14]);
+      L[15] = m2l_fma(-D[25], m, L[15]);
+      L[16] = m2l_fma(-D[26], m, L[16]);
+      L[17] = m2l_fma(-D[27], m, L[17]);
+      L[18] = m2l_fma(-D[28], m, L[18]);
+      L[19] = m2l_fma(-D[29], m, L[19]);
+      L[20] = m2l_fma(D[35], m, L[20]);
+      L[21] = m2l_fma(D[36], m, L[21]);
+      L[22] = m2l_fma(D[37], m, L[22]);
+      L[23] = m2l_fma(D[38], m, L[23]);
+      L[24] = m2l_fma(D[39], m, L[24]);
+      L[25] = m2l_fma(D[40], m, L[25]);
+      L[26] = m2l_fma(D[41], m, L[26]);
+      L[27] = m2l_fma(D[42], m, L[27]);
+      L[28] = m2l_fma(D[43], m, L[28]);
+      L[29] = m2l_fma(D[44], m, L[29]);
+      L[30] = m2l_fma(D[45], m, L[30]);
+      L[31] = m2l_fma(D[46], m, L[31]);
+      L[32] = m2l_fma(D[47], m, L[32]);
+      L[33] = m2l_fma(D[48], m, L[33]);
+      L[34] = m2l_fma(D[49], m, L[34]);
     }
-    { const float m = __ldg(Ms + 2);
-      L[0] = fmaf(D[2], m, L[0]);
-      L[1] = fmaf(-D[5], m, L[1]);
-      L[2] = fmaf(-D[7], m, L[2]);
-      L[3] = fmaf(-D[8], m, L[3]);
-      L[4] = fmaf(D[11], m, L[4]);
-      L[5] = fmaf(D[13], m, L[5]);
-      L[6] = fmaf(D[14], m, L[6]);
-      L[7] = fmaf(D[16], m, L[7]);
-      L[8] = fmaf(D[17], m, L[8]);
-      L[9] = fmaf(D[18], m, L[9]);
-      L[10] = fmaf(-D[21], m, L[10]);
-      L[11] = fmaf(-D[23], m, L[11]);
-      L[12] = fmaf(-D[24], m, L[12]);
-      L[13] = fmaf(-D[26], m, L[13]);
-      L[14] = fmaf(-D[27], m, L[14]);
-      L[15] = fmaf(-D[28], m, L[15]);
-      L[16] = fmaf(-D[30], m, L[16]);
-      L[17] = fmaf(-D[31], m, L[17]);
-      L[18] = fmaf(-D[32], m, L[18]);
-      L[19] = fmaf(-D[33], m, L[19]);
-      L[20] = fmaf(D[36], m, L[20]);
-      L[21] = fmaf(D[38], m, L[21]);
-      L[22] = fmaf(D[39], m, L[22]);
-      L[23] = fmaf(D[41], m, L[23]);
-      L[24] = fmaf(D[42], m, L[24]);
-      L[25] = fmaf(D[43], m, L[25]);
-      L[26] = fmaf(D[45], m, L[26]);
-      L[27] = fmaf(D[46], m, L[27]);
-      L[28] = fmaf(D[47], m, L[28]);
-      L[29] = fmaf(D[48], m, L[29]);
-      L[30] = fmaf(D[50], m, L[30]);
-      L[31] = fmaf(D[51], m, L[31]);
-      L[32] = fmaf(D[52], m, L[32]);
-      L[33] = fmaf(D[53], m, L[33]);
-      L[34] = fmaf(D[54], m, L[34]);
+    { const T m = __ldg(Ms + 2);
+      L[0] = m2l_fma(D[2], m, L[0]);
+      L[1] = m2l_fma(-D[5], m, L[1]);
+      L[2] = m2l_fma(-D[7], m, L[2]);
+      L[3] = m2l_fma(-D[8], m, L[3]);
+      L[4] = m2l_fma(D[11], m, L[4]);
+      L[5] = m2l_fma(D[13], m, L[5]);
+      L[6] = m2l_fma(D[14], m, L[6]);
+      L[7] = m2l_fma(D[16], m, L[7]);
+      L[8] = m2l_fma(D[17], m, L[8]);
+      L[9] = m2l_fma(D[18], m, L[9]);
+      L[10] = m2l_fma(-D[21], m, L[10]);
+      L[11] = m2l_fma(-D[23], m, L[11]);
+      L[12] = m2l_fma(-D[24], m, L[12]);
+      L[13] = m2l_fma(-D[26], m, L[13]);
+      L[14] = m2l_fma(-D[27], m, L[14]);
+      L[15] = m2l_fma(-D[28], m, L[15]);
+      L[16] = m2l_fma(-D[30], m, L[16]);
+      L[17] = m2l_fma(-D[31], m, L[17]);
+      L[18] = m2l_fma(-D[32], m, L[18]);
+      L[19] = m2l_fma(-D[33], m, L[19]);
+      L[20] = m2l_fma(D[36], m, L[20]);
+      L[21] = m2l_fma(D[38], m, L[21]);
+      L[22] = m2l_fma(D[39], m, L[22]);
+      L[23] = m2l_fma(D[41], m, L[23]);
+      L[24] = m2l_fma(D[42], m, L[24]);
+      L[25] = m2l_fma(D[43], m, L[25]);
+      L[26] = m2l_fma(D[45], m, L[26]);
+      L[27] = m2l_fma(D[46], m, L[27]);
+      L[28] = m2l_fma(D[47], m, L[28]);
+      L[29] = m2l_fma(D[48], m, L[29]);
+      L[30] = m2l_fma(D[50], m, L[30]);
+      L[31] = m2l_fma(D[51], m, L[31]);
+      L[32] = m2l_fma(D[52], m, L[32]);
+      L[33] = m2l_fma(D[53], m, L[33]);
+      L[34] = m2l_fma(D[54], m, L[34]);
     }
-    { const float m = __ldg(Ms + 3);
-      L[0] = fmaf(D[3], m, L[0]);
-      L[1] = fmaf(-D[6], m, L[1]);
-      L[2] = fmaf(-D[8], m, L[2]);
-      L[3] = fmaf(-D[9], m, L[3]);
-      L[4] = fmaf(D[12], m, L[4]);
-      L[5] = fmaf(D[14], m, L[5]);
-      L[6] = fmaf(D[15], m, L[6]);
-      L[7] = fmaf(D[17], m, L[7]);
-      L[8] = fmaf(D[18], m, L[8]);
-      L[9] = fmaf(D[19], m, L[9]);
-      L[10] = fmaf(-D[22], m, L[10]);
-      L[11] = fmaf(-D[24], m, L[11]);
-      L[12] = fmaf(-D[25], m, L[12]);
-      L[13] = fmaf(-D[27], m, L[13]);
-      L[14] = fmaf(-D[28], m, L[14]);
-      L[15] = fmaf(-D[29], m, L[15]);
-      L[16] = fmaf(-D[31], m, L[16]);
-      L[17] = fmaf(-D[32], m, L[17]);
-      L[18] = fmaf(-D[33], m, L[18]);
-      L[19] = fmaf(-D[34], m, L[19]);
-      L[20] = fmaf(D[37], m, L[20]);
-      L[21] = fmaf(D[39], m, L[21]);
-      L[22] = fmaf(D[40], m, L[22]);
-      L[23] = fmaf(D[42], m, L[23]);
-      L[24] = fmaf(D[43], m, L[24]);
-      L[25] = fmaf(D[44], m, L[25]);
-      L[26] = fmaf(D[46], m, L[26]);
-      L[27] = fmaf(D[47], m, L[27]);
-      L[28] = fmaf(D[48], m, L[28]);
-      L[29] = fmaf(D[49], m, L[29]);
-      L[30] = fmaf(D[51], m, L[30]);
-      L[31] = fmaf(D[52], m, L[31]);
-      L[32] = fmaf(D[53], m, L[32]);
-      L[33] = fmaf(D[54], m, L[33]);
-      L[34] = fmaf(D[55], m, L[34]);
+    { const T m = __ldg(Ms + 3);
+      L[0] = m2l_fma(D[3], m, L[0]);
+      L[1] = m2l_fma(-D[6], m, L[1]);
+      L[2] = m2l_fma(-D[8], m, L[2]);
+      L[3] = m2l_fma(-D[9], m, L[3]);
+      L[4] = m2l_fma(D[12], m, L[4]);
+      L[5] = m2l_fma(D[14], m, L[5]);
+      L[6] = m2l_fma(D[15], m, L[6]);
+      L[7] = m2l_fma(D[17], m, L[7]);
+      L[8] = m2l_fma(D[18], m, L[8]);
+      L[9] = m2l_fma(D[19], m, L[9]);
+      L[10] = m2l_fma(-D[22], m, L[10]);
+      L[11] = m2l_fma(-D[24], m, L[11]);
+      L[12] = m2l_fma(-D[25], m, L[12]);
+      L[13] = m2l_fma(-D[27], m, L[13]);
+      L[14] = m2l_fma(-D[28], m, L[14]);
+      L[15] = m2l_fma(-D[29], m, L[15]);
+      L[16] = m2l_fma(-D[31], m, L[16]);
+      L[17] = m2l_fma(-D[32], m, L[17]);
+      L[18] = m2l_fma(-D[33], m, L[18]);
+      L[19] = m2l_fma(-D[34], m, L[19]);
+      L[20] = m2l_fma(D[37], m, L[20]);
+      L[21] = m2l_fma(D[39], m, L[21]);
+      L[22] = m2l_fma(D[40], m, L[22]);
+      L[23] = m2l_fma(D[42], m, L[23]);
+      L[24] = m2l_fma(D[43], m, L[24]);
+      L[25] = m2l_fma(D[44], m, L[25]);
+      L[26] = m2l_fma(D[46], m, L[26]);
+      L[27] = m2l_fma(D[47], m, L[27]);
+      L[28] = m2l_fma(D[48], m, L[28]);
+      L[29] = m2l_fma(D[49], m, L[29]);
+      L[30] = m2l_fma(D[51], m, L[30]);
+      L[31] = m2l_fma(D[52], m, L[31]);
+      L[32] = m2l_fma(D[53], m, L[32]);
+      L[33] = m2l_fma(D[54], m, L[33]);
+      L[34] = m2l_fma(D[55], m, L[34]);
     }
-    { const float m = __ldg(Ms + 4);
-      L[0] = fmaf(D[4], m, L[0]);
-      L[1] = fmaf(-D[10], m, L[1]);
-      L[2] = fmaf(-D[11], m, L[2]);
-      L[3] = fmaf(-D[12], m, L[3]);
-      L[4] = fmaf(D[20], m, L[4]);
-      L[5] = fmaf(D[21], m, L[5]);
-      L[6] = fmaf(D[22], m, L[6]);
-      L[7] = fmaf(D[23], m, L[7]);
-      L[8] = fmaf(D[24], m, L[8]);
-      L[9] = fmaf(D[25], m, L[9]);
-      L[10] = fmaf(-D[35], m, L[10]);
-      L[11] = fmaf(-D[36], m, L[11]);
-      L[12] = fmaf(-D[37], m, L[12]);
-      L[13] = fmaf(-D[38], m, L[13]);
-      L[14] = fmaf(-D[39], m, L[14]);
-      L[15] = fmaf(-D[40], m, L[15]);
-      L[16] = fmaf(-D[41], m, L[16]);
-      L[17] = fmaf(-D[42], m, L[17]);
-      L[18] = fmaf(-D[43], m, L[18]);
-      L[19] = fmaf(-D[44], m, L[19]);
+    { const T m = __ldg(Ms + 4);
+      L[0] = m2l_fma(D[4], m, L[0]);
+      L[1] = m2l_fma(-D[10], m, L[1]);
+      L[2] = m2l_fma(-D[11], m, L[2]);
+      L[3] = m2l_fma(-D[12], m, L[3]);
+      L[4] = m2l_fma(D[20], m, L[4]);
+      L[5] = m2l_fma(D[21], m, L[5]);
+      L[6] = m2l_fma(D[22], m, L[6]);
+      L[7] = m2l_fma(D[23], m, L[7]);
+      L[8] = m2l_fma(D[24], m, L[8]);
+      L[9] = m2l_fma(D[25], m, L[9]);
+      L[10] = m2l_fma(-D[35], m, L[10]);
+      L[11] = m2l_fma(-D[36], m, L[11]);
+      L[12] = m2l_fma(-D[37], m, L[12]);
+      L[13] = m2l_fma(-D[38], m, L[13]);
+      L[14] = m2l_fma(-D[39], m, L[14]);
+      L[15] = m2l_fma(-D[40], m, L[15]);
+      L[16] = m2l_fma(-D[41], m, L[16]);
+      L[17] = m2l_fma(-D[42], m, L[17]);
+      L[18] = m2l_fma(-D[43], m, L[18]);
+      L[19] = m2l_fma(-D[44], m, L[19]);
     }
-    { const float m = __ldg(Ms + 5);
-      L[0] = fmaf(D[5], m, L[0]);
-      L[1] = fmaf(-D[11], m, L[1]);
-      L[2] = fmaf(-D[13], m, L[2]);
-      L[3] = fmaf(-D[14], m, L[3]);
-      L[4] = fmaf(D[21], m, L[4]);
-      L[5] = fmaf(D[23], m, L[5]);
-      L[6] = fmaf(D[24], m, L[6]);
-      L[7] = fmaf(D[26], m, L[7]);
-      L[8] = fmaf(D[27], m, L[8]);
-      L[9] = fmaf(D[28], m, L[9]);
-      L[10] = fmaf(-D[36], m, L[10]);
-      L[11] = fmaf(-D[38], m, L[11]);
-      L[12] = fmaf(-D[39], m, L[12]);
-      L[13] = fmaf(-D[41], m, L[13]);
-      L[14] = fmaf(-D[42], m, L[14]);
-      L[15] = fmaf(-D[43], m, L[15]);
-      L[16] = fmaf(-D[45], m, L[16]);
-      L[17] = fmaf(-D[46], m, L[17]);
-      L[18] = fmaf(-D[47], m, L[18]);
-      L[19] = fmaf(-D[48], m, L[19]);
+    { const T m = __ldg(Ms + 5);
+      L[0] = m2l_fma(D[5], m, L[0]);
+      L[1] = m2l_fma(-D[11], m, L[1]);
+      L[2] = m2l_fma(-D[13], m, L[2]);
+      L[3] = m2l_fma(-D[14], m, L[3]);
+      L[4] = m2l_fma(D[21], m, L[4]);
+      L[5] = m2l_fma(D[23], m, L[5]);
+      L[6] = m2l_fma(D[24], m, L[6]);
+      L[7] = m2l_fma(D[26], m, L[7]);
+      L[8] = m2l_fma(D[27], m, L[8]);
+      L[9] = m2l_fma(D[28], m, L[9]);
+      L[10] = m2l_fma(-D[36], m, L[10]);
+      L[11] = m2l_fma(-D[38], m, L[11]);
+      L[12] = m2l_fma(-D[39], m, L[12]);
+      L[13] = m2l_fma(-D[41], m, L[13]);
+      L[14] = m2l_fma(-D[42], m, L[14]);
+      L[15] = m2l_fma(-D[43], m, L[15]);
+      L[16] = m2l_fma(-D[45], m, L[16]);
+      L[17] = m2l_fma(-D[46], m, L[17]);
+      L[18] = m2l_fma(-D[47], m, L[18]);
+      L[19] = m2l_fma(-D[48], m, L[19]);
     }
-    { const float m = __ldg(Ms + 6);
-      L[0] = fmaf(D[6], m, L[0]);
-      L[1] = fmaf(-D[12], m, L[1]);
-      L[2] = fmaf(-D[14], m, L[2]);
-      L[3] = fmaf(-D[15], m, L[3]);
-      L[4] = fmaf(D[22], m, L[4]);
-      L[5] = fmaf(D[24], m, L[5]);
-      L[6] = fmaf(D[25], m, L[6]);
-      L[7] = fmaf(D[27], m, L[7]);
-      L[8] = fmaf(D[28], m, L[8]);
-      L[9] = fmaf(D[29], m, L[9]);
-      L[10] = fmaf(-D[37], m, L[10]);
-      L[11] = fmaf(-D[39], m, L[11]);
-      L[12] = fmaf(-D[40], m, L[12]);
-      L[13] = fmaf(-D[42], m, L[13]);
-      L[14] = fmaf(-D[43], m, L[14]);
-      L[15] = fmaf(-D[44], m, L[15]);
-      L[16] = fmaf(-D[46], m, L[16]);
-      L[17] = fmaf(-D[47], m, L[17]);
-      L[18] = fmaf(-D[48], m, L[18]);
-      L[19] = fmaf(-D[49], m, L[19]);
+    { const T m = __ldg(Ms + 6);
+      L[0] = m2l_fma(D[6], m, L[0]);
+      L[1] = m2l_fma(-D[12], m, L[1]);
+      L[2] = m2l_fma(-D[14], m, L[2]);
+      L[3] = m2l_fma(-D[15], m, L[3]);
+      L[4] = m2l_fma(D[22], m, L[4]);
+      L[5] = m2l_fma(D[24], m, L[5]);
+      L[6] = m2l_fma(D[25], m, L[6]);
+      L[7] = m2l_fma(D[27], m, L[7]);
+      L[8] = m2l_fma(D[28], m, L[8]);
+      L[9] = m2l_fma(D[29], m, L[9]);
+      L[10] = m2l_fma(-D[37], m, L[10]);
+      L[11] = m2l_fma(-D[39], m, L[11]);
+      L[12] = m2l_fma(-D[40], m, L[12]);
+      L[13] = m2l_fma(-D[42], m, L[13]);
+      L[14] = m2l_fma(-D[43], m, L[14]);
+      L[15] = m2l_fma(-D[44], m, L[15]);
+      L[16] = m2l_fma(-D[46], m, L[16]);
+      L[17] = m2l_fma(-D[47], m, L[17]);
+      L[18] = m2l_fma(-D[48], m, L[18]);
+      L[19] = m2l_fma(-D[49], m, L[19]);
     }
-    { const float m = __ldg(Ms + 7);
-      L[0] = fmaf(D[7], m, L[0]);
-      L[1] = fmaf(-D[13], m, L[1]);
-      L[2] = fmaf(-D[16], m, L[2]);
-      L[3] = fmaf(-D[17], m, L[3]);
-      L[4] = fmaf(D[23], m, L[4]);
-      L[5] = fmaf(D[26], m, L[5]);
-      L[6] = fmaf(D[27], m, L[6]);
-      L[7] = fmaf(D[30], m, L[7]);
-      L[8] = fmaf(D[31], m, L[8]);
-      L[9] = fmaf(D[32], m, L[9]);
-      L[10] = fmaf(-D[38], m, L[10]);
-      L[11] = fmaf(-D[41], m, L[11]);
-      L[12] = fmaf(-D[42], m, L[12]);
-      L[13] = fmaf(-D[45], m, L[13]);
-      L[14] = fmaf(-D[46], m, L[14]);
-      L[15] = fmaf(-D[47], m, L[15]);
-      L[16] = fmaf(-D[50], m, L[16]);
-      L[17] = fmaf(-D[51], m, L[17]);
-      L[18] = fmaf(-D[52], m, L[18]);
-      L[19] = fmaf(-D[53], m, L[19]);
+    { const T m = __ldg(Ms + 7);
+      L[0] = m2l_fma(D[7], m, L[0]);
+      L[1] = m2l_fma(-D[13], m, L[1]);
+      L[2] = m2l_fma(-D[16], m, L[2]);
+      L[3] = m2l_fma(-D[17], m, L[3]);
+      L[4] = m2l_fma(D[23], m, L[4]);
+      L[5] = m2l_fma(D[26], m, L[5]);
+      L[6] = m2l_fma(D[27], m, L[6]);
+      L[7] = m2l_fma(D[30], m, L[7]);
+      L[8] = m2l_fma(D[31], m, L[8]);
+      L[9] = m2l_fma(D[32], m, L[9]);
+      L[10] = m2l_fma(-D[38], m, L[10]);
+      L[11] = m2l_fma(-D[41], m, L[11]);
+      L[12] = m2l_fma(-D[42], m, L[12]);
+      L[13] = m2l_fma(-D[45], m, L[13]);
+      L[14] = m2l_fma(-D[46], m, L[14]);
+      L[15] = m2l_fma(-D[47], m, L[15]);
+      L[16] = m2l_fma(-D[50], m, L[16]);
+      L[17] = m2l_fma(-D[51], m, L[17]);
+      L[18] = m2l_fma(-D[52], m, L[18]);
+      L[19] = m2l_fma(-D[53], m, L[19]);
     }
-    { const float m = __ldg(Ms + 8);
-      L[0] = fmaf(D[8], m, L[0]);
-      L[1] = fmaf(-D[14], m, L[1]);
-      L[2] = fmaf(-D[17], m, L[2]);
-      L[3] = fmaf(-D[18], m, L[3]);
-      L[4] = fmaf(D[24], m, L[4]);
-      L[5] = fmaf(D[27], m, L[5]);
-      L[6] = fmaf(D[28], m, L[6]);
-      L[7] = fmaf(D[31], m, L[7]);
-      L[8] = fmaf(D[32], m, L[8]);
-      L[9] = fmaf(D[33], m, L[9]);
-      L[10] = fmaf(-D[39], m, L[10]);
-      L[11] = fmaf(-D[42], m, L[11]);
-      L[12] = fmaf(-D[43], m, L[12]);
-      L[13] = fmaf(-D[46], m, L[13]);
-      L[14] = fmaf(-D[47], m, L[14]);
-      L[15] = fmaf(-D[48], m, L[15]);
-      L[16] = fmaf(-D[51], m, L[16]);
-      L[17] = fmaf(-D[52], m, L[17]);
-      L[18] = fmaf(-D[53], m, L[18]);
-      L[19] = fmaf(-D[54], m, L[19]);
+    { const T m = __ldg(Ms + 8);
+      L[0] = m2l_fma(D[8], m, L[0]);
+      L[1] = m2l_fma(-D[14], m, L[1]);
+      L[2] = m2l_fma(-D[17], m, L[2]);
+      L[3] = m2l_fma(-D[18], m, L[3]);
+      L[4] = m2l_fma(D[24], m, L[4]);
+      L[5] = m2l_fma(D[27], m, L[5]);
+      L[6] = m2l_fma(D[28], m, L[6]);
+      L[7] = m2l_fma(D[31], m, L[7]);
+      L[8] = m2l_fma(D[32], m, L[8]);
+      L[9] = m2l_fma(D[33], m, L[9]);
+      L[10] = m2l_fma(-D[39], m, L[10]);
+      L[11] = m2l_fma(-D[42], m, L[11]);
+      L[12] = m2l_fma(-D[43], m, L[12]);
+      L[13] = m2l_fma(-D[46], m, L[13]);
+      L[14] = m2l_fma(-D[47], m, L[14]);
+      L[15] = m2l_fma(-D[48], m, L[15]);
+      L[16] = m2l_fma(-D[51], m, L[16]);
+      L[17] = m2l_fma(-D[52], m, L[17]);
+      L[18] = m2l_fma(-D[53], m, L[18]);
+      L[19] = m2l_fma(-D[54], m, L[19]);
     }
-    { const float m = __ldg(Ms + 9);
-      L[0] = fmaf(D[9], m, L[0]);
-      L[1] = fmaf(-D[15], m, L[1]);
-      L[2] = fmaf(-D[18], m, L[2]);
-      L[3] = fmaf(-D[19], m, L[3]);
-      L[4] = fmaf(D[25], m, L[4]);
-      L[5] = fmaf(D[28], m, L[5]);
-      L[6] = fmaf(D[29], m, L[6]);
-      L[7] = fmaf(D[32], m, L[7]);
-      L[8] = fmaf(D[33], m, L[8]);
-      L[9] = fmaf(D[34], m, L[9]);
-      L[10] = fmaf(-D[40], m, L[10]);
-      L[11] = fmaf(-D[43], m, L[11]);
-      L[12] = fmaf(-D[44], m, L[12]);
-      L[13] = fmaf(-D[47], m, L[13]);
-      L[14] = fmaf(-D[48], m, L[14]);
-      L[15] = fmaf(-D[49], m, L[15]);
-      L[16] = fmaf(-D[52], m, L[16]);
-      L[17] = fmaf(-D[53], m, L[17]);
-      L[18] = fmaf(-D[54], m, L[18]);
-      L[19] = fmaf(-D[55], m, L[19]);
+    { const T m = __ldg(Ms + 9);
+      L[0] = m2l_fma(D[9], m, L[0]);
+      L[1] = m2l_fma(-D[15], m, L[1]);
+      L[2] = m2l_fma(-D[18], m, L[2]);
+      L[3] = m2l_fma(-D[19], m, L[3]);
+      L[4] = m2l_fma(D[25], m, L[4]);
+      L[5] = m2l_fma(D[28], m, L[5]);
+      L[6] = m2l_fma(D[29], m, L[6]);
+      L[7] = m2l_fma(D[32], m, L[7]);
+      L[8] = m2l_fma(D[33], m, L[8]);
+      L[9] = m2l_fma(D[34], m, L[9]);
+      L[10] = m2l_fma(-D[40], m, L[10]);
+      L[11] = m2l_fma(-D[43], m, L[11]);
+      L[12] = m2l_fma(-D[44], m, L[12]);
+      L[13] = m2l_fma(-D[47], m, L[13]);
+      L[14] = m2l_fma(-D[48], m, L[14]);
+      L[15] = m2l_fma(-D[49], m, L[15]);
+      L[16] = m2l_fma(-D[52], m, L[16]);
+      L[17] = m2l_fma(-D[53], m, L[17]);
+      L[18] = m2l_fma(-D[54], m, L[18]);
+      L[19] = m2l_fma(-D[55], m, L[19]);
     }
-    { const float m = __ldg(Ms + 10);
-      L[0] = fmaf(D[10], m, L[0]);
-      L[1] = fmaf(-D[20], m, L[1]);
-      L[2] = fmaf(-D[21], m, L[2]);
-      L[3] = fmaf(-D[22], m, L[3]);
-      L[4] = fmaf(D[35], m, L[4]);
-      L[5] = fmaf(D[36], m, L[5]);
-      L[6] = fmaf(D[37], m, L[6]);
-      L[7] = fmaf(D[38], m, L[7]);
-      L[8] = fmaf(D[39], m, L[8]);
-      L[9] = fmaf(D[40], m, L[9]);
+    { const T m = __ldg(Ms + 10);
+      L[0] = m2l_fma(D[10], m, L[0]);
+      L[1] = m2l_fma(-D[20], m, L[1]);
+      L[2] = m2l_fma(-D[21], m, L[2]);
+      L[3] = m2l_fma(-D[22], m, L[3]);
+      L[4] = m2l_fma(D[35], m, L[4]);
+      L[5] = m2l_fma(D[36], m, L[5]);
+      L[6] = m2l_fma(D[37], m, L[6]);
+      L[7] = m2l_fma(D[38], m, L[7]);
+      L[8] = m2l_fma(D[39], m, L[8]);
+      L[9] = m2l_fma(D[40], m, L[9]);
     }
-    { const float m = __ldg(Ms + 11);
-      L[0] = fmaf(D[11], m, L[0]);
-      L[1] = fmaf(-D[21], m, L[1]);
-      L[2] = fmaf(-D[23], m, L[2]);
-      L[3] = fmaf(-D[24], m, L[3]);
-      L[4] = fmaf(D[36], m, L[4]);
-      L[5] = fmaf(D[38], m, L[5]);
-      L[6] = fmaf(D[39], m, L[6]);
-      L[7] = fmaf(D[41], m, L[7]);
-      L[8] = fmaf(D[42], m, L[8]);
-      L[9] = fmaf(D[43], m, L[9]);
+    { const T m = __ldg(Ms + 11);
+      L[0] = m2l_fma(D[11], m, L[0]);
+      L[1] = m2l_fma(-D[21], m, L[1]);
+      L[2] = m2l_fma(-D[23], m, L[2]);
+      L[3] = m2l_fma(-D[24], m, L[3]);
+      L[4] = m2l_fma(D[36], m, L[4]);
+      L[5] = m2l_fma(D[38], m, L[5]);
+      L[6] = m2l_fma(D[39], m, L[6]);
+      L[7] = m2l_fma(D[41], m, L[7]);
+      L[8] = m2l_fma(D[42], m, L[8]);
+      L[9] = m2l_fma(D[43], m, L[9]);
     }
-    { const float m = __ldg(Ms + 12);
-      L[0] = fmaf(D[12], m, L[0]);
-      L[1] = fmaf(-D[22], m, L[1]);
-      L[2] = fmaf(-D[24], m, L[2]);
-      L[3] = fmaf(-D[25], m, L[3]);
-      L[4] = fmaf(D[37], m, L[4]);
-      L[5] = fmaf(D[39], m, L[5]);
-      L[6] = fmaf(D[40], m, L[6]);
-      L[7] = fmaf(D[42], m, L[7]);
-      L[8] = fmaf(D[43], m, L[8]);
-      L[9] = fmaf(D[44], m, L[9]);
+    { const T m = __ldg(Ms + 12);
+      L[0] = m2l_fma(D[12], m, L[0]);
+      L[1] = m2l_fma(-D[22], m, L[1]);
+      L[2] = m2l_fma(-D[24], m, L[2]);
+      L[3] = m2l_fma(-D[25], m, L[3]);
+      L[4] = m2l_fma(D[37], m, L[4]);
+      L[5] = m2l_fma(D[39], m, L[5]);
+      L[6] = m2l_fma(D[40], m, L[6]);
+      L[7] = m2l_fma(D[42], m, L[7]);
+      L[8] = m2l_fma(D[43], m, L[8]);
+      L[9] = m2l_fma(D[44], m, L[9]);
     }
-    { const float m = __ldg(Ms + 13);
-      L[0] = fmaf(D[13], m, L[0]);
-      L[1] = fmaf(-D[23], m, L[1]);
-      L[2] = fmaf(-D[26], m, L[2]);
-      L[3] = fmaf(-D[27], m, L[3]);
-      L[4] = fmaf(D[38], m, L[4]);
-      L[5] = fmaf(D[41], m, L[5]);
-      L[6] = fmaf(D[42], m, L[6]);
-      L[7] = fmaf(D[45], m, L[7]);
-      L[8] = fmaf(D[46], m, L[8]);
-      L[9] = fmaf(D[47], m, L[9]);
+    { const T m = __ldg(Ms + 13);
+      L[0] = m2l_fma(D[13], m, L[0]);
+      L[1] = m2l_fma(-D[23], m, L[1]);
+      L[2] = m2l_fma(-D[26], m, L[2]);
+      L[3] = m2l_fma(-D[27], m, L[3]);
+      L[4] = m2l_fma(D[38], m, L[4]);
+      L[5] = m2l_fma(D[41], m, L[5]);
+      L[6] = m2l_fma(D[42], m, L[6]);
+      L[7] = m2l_fma(D[45], m, L[7]);
+      L[8] = m2l_fma(D[46], m, L[8]);
+      L[9] = m2l_fma(D[47], m, L[9]);
     }
-    { const float m = __ldg(Ms + 14);
-      L[0] = fmaf(D[14], m, L[0]);
-      L[1] = fmaf(-D[24], m, L[1]);
-      L[2] = fmaf(-D[27], m, L[2]);
-      L[3] = fmaf(-D[28], m, L[3]);
-      L[4] = fmaf(D[39], m, L[4]);
-      L[5] = fmaf(D[42], m, L[5]);
-      L[6] = fmaf(D[43], m, L[6]);
-      L[7] = fmaf(D[46], m, L[7]);
-      L[8] = fmaf(D[47], m, L[8]);
-      L[9] = fmaf(D[48], m, L[9]);
+    { const T m = __ldg(Ms + 14);
+      L[0] = m2l_fma(D[14], m, L[0]);
+      L[1] = m2l_fma(-D[24], m, L[1]);
+      L[2] = m2l_fma(-D[27], m, L[2]);
+      L[3] = m2l_fma(-D[28], m, L[3]);
+      L[4] = m2l_fma(D[39], m, L[4]);
+      L[5] = m2l_fma(D[42], m, L[5]);
+      L[6] = m2l_fma(D[43], m, L[6]);
+      L[7] = m2l_fma(D[46], m, L[7]);
+      L[8] = m2l_fma(D[47], m, L[8]);
+      L[9] = m2l_fma(D[48], m, L[9]);
     }
-    { const float m = __ldg(Ms + 15);
-      L[0] = fmaf(D[15], m, L[0]);
-      L[1] = fmaf(-D[25], m, L[1]);
-      L[2] = fmaf(-D[28], m, L[2]);
-      L[3] = fmaf(-D[29], m, L[3]);
-      L[4] = fmaf(D[40], m, L[4]);
-      L[5] = fmaf(D[43], m, L[5]);
-      L[6] = fmaf(D[44], m, L[6]);
-      L[7] = fmaf(D[47], m, L[7]);
-      L[8] = fmaf(D[48], m, L[8]);
-      L[9] = fmaf(D[49], m, L[9]);
+    { const T m = __ldg(Ms + 15);
+      L[0] = m2l_fma(D[15], m, L[0]);
+      L[1] = m2l_fma(-D[25], m, L[1]);
+      L[2] = m2l_fma(-D[28], m, L[2]);
+      L[3] = m2l_fma(-D[29], m, L[3]);
+      L[4] = m2l_fma(D[40], m, L[4]);
+      L[5] = m2l_fma(D[43], m, L[5]);
+      L[6] = m2l_fma(D[44], m, L[6]);
+      L[7] = m2l_fma(D[47], m, L[7]);
+      L[8] = m2l_fma(D[48], m, L[8]);
+      L[9] = m2l_fma(D[49], m, L[9]);
     }
-    { const float m = __ldg(Ms + 16);
-      L[0] = fmaf(D[16], m, L[0]);
-      L[1] = fmaf(-D[26], m, L[1]);
-      L[2] = fmaf(-D[30], m, L[2]);
-      L[3] = fmaf(-D[31], m, L[3]);
-      L[4] = fmaf(D[41], m, L[4]);
-      L[5] = fmaf(D[45], m, L[5]);
-      L[6] = fmaf(D[46], m, L[6]);
-      L[7] = fmaf(D[50], m, L[7]);
-      L[8] = fmaf(D[51], m, L[8]);
-      L[9] = fmaf(D[52], m, L[9]);
+    { const T m = __ldg(Ms + 16);
+      L[0] = m2l_fma(D[16], m, L[0]);
+      L[1] = m2l_fma(-D[26], m, L[1]);
+      L[2] = m2l_fma(-D[30], m, L[2]);
+      L[3] = m2l_fma(-D[31], m, L[3]);
+      L[4] = m2l_fma(D[41], m, L[4]);
+      L[5] = m2l_fma(D[45], m, L[5]);
+      L[6] = m2l_fma(D[46], m, L[6]);
+      L[7] = m2l_fma(D[50], m, L[7]);
+      L[8] = m2l_fma(D[51], m, L[8]);
+      L[9] = m2l_fma(D[52], m, L[9]);
     }
-    { const float m = __ldg(Ms + 17);
-      L[0] = fmaf(D[17], m, L[0]);
-      L[1] = fmaf(-D[27], m, L[1]);
-      L[2] = fmaf(-D[31], m, L[2]);
-      L[3] = fmaf(-D[32], m, L[3]);
-      L[4] = fmaf(D[42], m, L[4]);
-      L[5] = fmaf(D[46], m, L[5]);
-      L[6] = fmaf(D[47], m, L[6]);
-      L[7] = fmaf(D[51], m, L[7]);
-      L[8] = fmaf(D[52], m, L[8]);
-      L[9] = fmaf(D[53], m, L[9]);
+    { const T m = __ldg(Ms + 17);
+      L[0] = m2l_fma(D[17], m, L[0]);
+      L[1] = m2l_fma(-D[27], m, L[1]);
+      L[2] = m2l_fma(-D[31], m, L[2]);
+      L[3] = m2l_fma(-D[32], m, L[3]);
+      L[4] = m2l_fma(D[42], m, L[4]);
+      L[5] = m2l_fma(D[46], m, L[5]);
+      L[6] = m2l_fma(D[47], m, L[6]);
+      L[7] = m2l_fma(D[51], m, L[7]);
+      L[8] = m2l_fma(D[52], m, L[8]);
+      L[9] = m2l_fma(D[53], m, L[9]);
     }
-    { const float m = __ldg(Ms + 18);
-      L[0] = fmaf(D[18], m, L[0]);
-      L[1] = fmaf(-D[28], m, L[1]);
-      L[2] = fmaf(-D[32], m, L[2]);
-      L[3] = fmaf(-D[33], m, L[3]);
-      L[4] = fmaf(D[43], m, L[4]);
-      L[5] = fmaf(D[47], m, L[5]);
-      L[6] = fmaf(D[48], m, L[6]);
-      L[7] = fmaf(D[52], m, L[7]);
-      L[8] = fmaf(D[53], m, L[8]);
-      L[9] = fmaf(D[54], m, L[9]);
+    { const T m = __ldg(Ms + 18);
+      L[0] = m2l_fma(D[18], m, L[0]);
+      L[1] = m2l_fma(-D[28], m, L[1]);
+      L[2] = m2l_fma(-D[32], m, L[2]);
+      L[3] = m2l_fma(-D[33], m, L[3]);
+      L[4] = m2l_fma(D[43], m, L[4]);
+      L[5] = m2l_fma(D[47], m, L[5]);
+      L[6] = m2l_fma(D[48], m, L[6]);
+      L[7] = m2l_fma(D[52], m, L[7]);
+      L[8] = m2l_fma(D[53], m, L[8]);
+      L[9] = m2l_fma(D[54], m, L[9]);
     }
-    { const float m = __ldg(Ms + 19);
-      L[0] = fmaf(D[19], m, L[0]);
-      L[1] = fmaf(-D[29], m, L[1]);
-      L[2] = fmaf(-D[33], m, L[2]);
-      L[3] = fmaf(-D[34], m, L[3]);
-      L[4] = fmaf(D[44], m, L[4]);
-      L[5] = fmaf(D[48], m, L[5]);
-      L[6] = fmaf(D[49], m, L[6]);
-      L[7] = fmaf(D[53], m, L[7]);
-      L[8] = fmaf(D[54], m, L[8]);
-      L[9] = fmaf(D[55], m, L[9]);
+    { const T m = __ldg(Ms + 19);
+      L[0] = m2l_fma(D[19], m, L[0]);
+      L[1] = m2l_fma(-D[29], m, L[1]);
+      L[2] = m2l_fma(-D[33], m, L[2]);
+      L[3] = m2l_fma(-D[34], m, L[3]);
+      L[4] = m2l_fma(D[44], m, L[4]);
+      L[5] = m2l_fma(D[48], m, L[5]);
+      L[6] = m2l_fma(D[49], m, L[6]);
+      L[7] = m2l_fma(D[53], m, L[7]);
+      L[8] = m2l_fma(D[54], m, L[8]);
+      L[9] = m2l_fma(D[55], m, L[9]);
     }
-    { const float m = __ldg(Ms + 20);
-      L[0] = fmaf(D[20], m, L[0]);
-      L[1] = fmaf(-D[35], m, L[1]);
-      L[2] = fmaf(-D[36], m, L[2]);
-      L[3] = fmaf(-D[37], m, L[3]);
+    { const T m = __ldg(Ms + 20);
+      L[0] = m2l_fma(D[20], m, L[0]);
+      L[1] = m2l_fma(-D[35], m, L[1]);
+      L[2] = m2l_fma(-D[36], m, L[2]);
+      L[3] = m2l_fma(-D[37], m, L[3]);
     }
-    { const float m = __ldg(Ms + 21);
-      L[0] = fmaf(D[21], m, L[0]);
-      L[1] = fmaf(-D[36], m, L[1]);
-      L[2] = fmaf(-D[38], m, L[2]);
-      L[3] = fmaf(-D[39], m, L[3]);
+    { const T m = __ldg(Ms + 21);
+      L[0] = m2l_fma(D[21], m, L[0]);
+      L[1] = m2l_fma(-D[36], m, L[1]);
+      L[2] = m2l_fma(-D[38], m, L[2]);
+      L[3] = m2l_fma(-D[39], m, L[3]);
     }
-    { const float m = __ldg(Ms + 22);
-      L[0] = fmaf(D[22], m, L[0]);
-      L[1] = fmaf(-D[37], m, L[1]);
-      L[2] = fmaf(-D[39], m, L[2]);
-      L[3] = fmaf(-D[40], m, L[3]);
+    { const T m = __ldg(Ms + 22);
+      L[0] = m2l_fma(D[22], m, L[0]);
+      L[1] = m2l_fma(-D[37], m, L[1]);
+      L[2] = m2l_fma(-D[39], m, L[2]);
+      L[3] = m2l_fma(-D[40], m, L[3]);
     }
-    { const float m = __ldg(Ms + 23);
-      L[0] = fmaf(D[23], m, L[0]);
-      L[1] = fmaf(-D[38], m, L[1]);
-      L[2] = fmaf(-D[41], m, L[2]);
-      L[3] = fmaf(-D[42], m, L[3]);
+    { const T m = __ldg(Ms + 23);
+      L[0] = m2l_fma(D[23], m, L[0]);
+      L[1] = m2l_fma(-D[38], m, L[1]);
+      L[2] = m2l_fma(-D[41], m, L[2]);
+      L[3] = m2l_fma(-D[42], m, L[3]);
     }
-    { const float m = __ldg(Ms + 24);
-      L[0] = fmaf(D[24], m, L[0]);
-      L[1] = fmaf(-D[39], m, L[1]);
-      L[2] = fmaf(-D[42], m, L[2]);
-      L[3] = fmaf(-D[43], m, L[3]);
+    { const T m = __ldg(Ms + 24);
+      L[0] = m2l_fma(D[24], m, L[0]);
+      L[1] = m2l_fma(-D[39], m, L[1]);
+      L[2] = m2l_fma(-D[42], m, L[2]);
+      L[3] = m2l_fma(-D[43], m, L[3]);
     }
-    { const float m = __ldg(Ms + 25);
-      L[0] = fmaf(D[25], m, L[0]);
-      L[1] = fmaf(-D[40], m, L[1]);
-      L[2] = fmaf(-D[43], m, L[2]);
-      L[3] = fmaf(-D[44], m, L[3]);
+    { const T m = __ldg(Ms + 25);
+      L[0] = m2l_fma(D[25], m, L[0]);
+      L[1] = m2l_fma(-D[40], m, L[1]);
+      L[2] = m2l_fma(-D[43], m, L[2]);
+      L[3] = m2l_fma(-D[44], m, L[3]);
     }
-    { const float m = __ldg(Ms + 26);
-      L[0] = fmaf(D[26], m, L[0]);
-      L[1] = fmaf(-D[41], m, L[1]);
-      L[2] = fmaf(-D[45], m, L[2]);
-      L[3] = fmaf(-D[46], m, L[3]);
+    { const T m = __ldg(Ms + 26);
+      L[0] = m2l_fma(D[26], m, L[0]);
+      L[1] = m2l_fma(-D[41], m, L[1]);
+      L[2] = m2l_fma(-D[45], m, L[2]);
+      L[3] = m2l_fma(-D[46], m, L[3]);
     }
-    { const float m = __ldg(Ms + 27);
-      L[0] = fmaf(D[27], m, L[0]);
-      L[1] = fmaf(-D[42], m, L[1]);
-      L[2] = fmaf(-D[46], m, L[2]);
-      L[3] = fmaf(-D[47], m, L[3]);
+    { const T m = __ldg(Ms + 27);
+      L[0] = m2l_fma(D[27], m, L[0]);
+      L[1] = m2l_fma(-D[42], m, L[1]);
+      L[2] = m2l_fma(-D[46], m, L[2]);
+      L[3] = m2l_fma(-D[47], m, L[3]);
     }
-    { const float m = __ldg(Ms + 28);
-      L[0] = fmaf(D[28], m, L[0]);
-      L[1] = fmaf(-D[43], m, L[1]);
-      L[2] = fmaf(-D[47], m, L[2]);
-      L[3] = fmaf(-D[48], m, L[3]);
+    { const T m = __ldg(Ms + 28);
+      L[0] = m2l_fma(D[28], m, L[0]);
+      L[1] = m2l_fma(-D[43], m, L[1]);
+      L[2] = m2l_fma(-D[47], m, L[2]);
+      L[3] = m2l_fma(-D[48], m, L[3]);
     }
-    { const float m = __ldg(Ms + 29);
-      L[0] = fmaf(D[29], m, L[0]);
-      L[1] = fmaf(-D[44], m, L[1]);
-      L[2] = fmaf(-D[48], m, L[2]);
-      L[3] = fmaf(-D[49], m, L[3]);
+    { const T m = __ldg(Ms + 29);
+      L[0] = m2l_fma(D[29], m, L[0]);
+      L[1] = m2l_fma(-D[44], m, L[1]);
+      L[2] = m2l_fma(-D[48], m, L[2]);
+      L[3] = m2l_fma(-D[49], m, L[3]);
     }
-    { const float m = __ldg(Ms + 30);
-      L[0] = fmaf(D[30], m, L[0]);
-      L[1] = fmaf(-D[45], m, L[1]);
-      L[2] = fmaf(-D[50], m, L[2]);
-      L[3] = fmaf(-D[51], m, L[3]);
+    { const T m = __ldg(Ms + 30);
+      L[0] = m2l_fma(D[30], m, L[0]);
+      L[1] = m2l_fma(-D[45], m, L[1]);
+      L[2] = m2l_fma(-D[50], m, L[2]);
+      L[3] = m2l_fma(-D[51], m, L[3]);
     }
-    { const float m = __ldg(Ms + 31);
-      L[0] = fmaf(D[31], m, L[0]);
-      L[1] = fmaf(-D[46], m, L[1]);
-      L[2] = fmaf(-D[51], m, L[2]);
-      L[3] = fmaf(-D[52], m, L[3]);
+    { const T m = __ldg(Ms + 31);
+      L[0] = m2l_fma(D[31], m, L[0]);
+      L[1] = m2l_fma(-D[46], m, L[1]);
+      L[2] = m2l_fma(-D[51], m, L[2]);
+      L[3] = m2l_fma(-D[52], m, L[3]);
     }
-    { const float m = __ldg(Ms + 32);
-      L[0] = fmaf(D[32], m, L[0]);
-      L[1] = fmaf(-D[47], m, L[1]);
-      L[2] = fmaf(-D[52], m, L[2]);
-      L[3] = fmaf(-D[53], m, L[3]);
+    { const T m = __ldg(Ms + 32);
+      L[0] = m2l_fma(D[32], m, L[0]);
+      L[1] = m2l_fma(-D[47], m, L[1]);
+      L[2] = m2l_fma(-D[52], m, L[2]);
+      L[3] = m2l_fma(-D[53], m, L[3]);
     }
-    { const float m = __ldg(Ms + 33);
-      L[0] = fmaf(D[33], m, L[0]);
-      L[1] = fmaf(-D[48], m, L[1]);
-      L[2] = fmaf(-D[53], m, L[2]);
-      L[3] = fmaf(-D[54], m, L[3]);
+    { const T m = __ldg(Ms + 33);
+      L[0] = m2l_fma(D[33], m, L[0]);
+      L[1] = m2l_fma(-D[48], m, L[1]);
+      L[2] = m2l_fma(-D[53], m, L[2]);
+      L[3] = m2l_fma(-D[54], m, L[3]);
     }
-    { const float m = __ldg(Ms + 34);
-      L[0] = fmaf(D[34], m, L[0]);
-      L[1] = fmaf(-D[49], m, L[1]);
-      L[2] = fmaf(-D[54], m, L[2]);
-      L[3] = fmaf(-D[55], m, L[3]);
+    { const T m = __ldg(Ms + 34);
+      L[0] = m2l_fma(D[34], m, L[0]);
+      L[1] = m2l_fma(-D[49], m, L[1]);
+      L[2] = m2l_fma(-D[54], m, L[2]);
+      L[3] = m2l_fma(-D[55], m, L[3]);
     }
-    { const float m = __ldg(Ms + 35);
-      L[0] = fmaf(D[35], m, L[0]);
+    { const T m = __ldg(Ms + 35);
+      L[0] = m2l_fma(D[35], m, L[0]);
     }
-    { const float m = __ldg(Ms + 36);
-      L[0] = fmaf(D[36], m, L[0]);
+    { const T m = __ldg(Ms + 36);
+      L[0] = m2l_fma(D[36], m, L[0]);
     }
-    { const float m = __ldg(Ms + 37);
-      L[0] = fmaf(D[37], m, L[0]);
+    { const T m = __ldg(Ms + 37);
+      L[0] = m2l_fma(D[37], m, L[0]);
     }
-    { const float m = __ldg(Ms + 38);
-      L[0] = fmaf(D[38], m, L[0]);
+    { const T m = __ldg(Ms + 38);
+      L[0] = m2l_fma(D[38], m, L[0]);
     }
-    { const float m = __ldg(Ms + 39);
-      L[0] = fmaf(D[39], m, L[0]);
+    { const T m = __ldg(Ms + 39);
+      L[0] = m2l_fma(D[39], m, L[0]);
     }
-    { const float m = __ldg(Ms + 40);
-      L[0] = fmaf(D[40], m, L[0]);
+    { const T m = __ldg(Ms + 40);
+      L[0] = m2l_fma(D[40], m, L[0]);
     }
-    { const float m = __ldg(Ms + 41);
-      L[0] = fmaf(D[41], m, L[0]);
+    { const T m = __ldg(Ms + 41);
+      L[0] = m2l_fma(D[41], m, L[0]);
     }
-    { const float m = __ldg(Ms + 42);
-      L[0] = fmaf(D[42], m, L[0]);
+    { const T m = __ldg(Ms + 42);
+      L[0] = m2l_fma(D[42], m, L[0]);
     }
-    { const float m = __ldg(Ms + 43);
-      L[0] = fmaf(D[43], m, L[0]);
+    { const T m = __ldg(Ms + 43);
+      L[0] = m2l_fma(D[43], m, L[0]);
     }
-    { const float m = __ldg(Ms + 44);
-      L[0] = fmaf(D[44], m, L[0]);
+    { const T m = __ldg(Ms + 44);
+      L[0] = m2l_fma(D[44], m, L[0]);
     }
-    { const float m = __ldg(Ms + 45);
-      L[0] = fmaf(D[45], m, L[0]);
+    { const T m = __ldg(Ms + 45);
+      L[0] = m2l_fma(D[45], m, L[0]);
     }
-    { const float m = __ldg(Ms + 46);
-      L[0] = fmaf(D[46], m, L[0]);
+    { const T m = __ldg(Ms + 46);
+      L[0] = m2l_fma(D[46], m, L[0]);
     }
-    { const float m = __ldg(Ms + 47);
-      L[0] = fmaf(D[47], m, L[0]);
+    { const T m = __ldg(Ms + 47);
+      L[0] = m2l_fma(D[47], m, L[0]);
     }
-    { const float m = __ldg(Ms + 48);
-      L[0] = fmaf(D[48], m, L[0]);
+    { const T m = __ldg(Ms + 48);
+      L[0] = m2l_fma(D[48], m, L[0]);
     }
-    { const float m = __ldg(Ms + 49);
-      L[0] = fmaf(D[49], m, L[0]);
+    { const T m = __ldg(Ms + 49);
+      L[0] = m2l_fma(D[49], m, L[0]);
     }
-    { const float m = __ldg(Ms + 50);
-      L[0] = fmaf(D[50], m, L[0]);
+    { const T m = __ldg(Ms + 50);
+      L[0] = m2l_fma(D[50], m, L[0]);
     }
-    { const float m = __ldg(Ms + 51);
-      L[0] = fmaf(D[51], m, L[0]);
+    { const T m = __ldg(Ms + 51);
+      L[0] = m2l_fma(D[51], m, L[0]);
     }
-    { const float m = __ldg(Ms + 52);
-      L[0] = fmaf(D[52], m, L[0]);
+    { const T m = __ldg(Ms + 52);
+      L[0] = m2l_fma(D[52], m, L[0]);
     }
-    { const float m = __ldg(Ms + 53);
-      L[0] = fmaf(D[53], m, L[0]);
+    { const T m = __ldg(Ms + 53);
+      L[0] = m2l_fma(D[53], m, L[0]);
     }
-    { const float m = __ldg(Ms + 54);
-      L[0] = fmaf(D[54], m, L[0]);
+    { const T m = __ldg(Ms + 54);
+      L[0] = m2l_fma(D[54], m, L[0]);
     }
-    { const float m = __ldg(Ms + 55);
-      L[0] = fmaf(D[55], m, L[0]);
+    { const T m = __ldg(Ms + 55);
+      L[0] = m2l_fma(D[55], m, L[0]);
     }
 }
 
-__device__ __forceinline__ void m2l_side_a_forces_5(const float (&D)[56], const float *__restrict__ Ms, float rho, float (&L)[56])
+template <class T> __device__ __forceinline__ void m2l_side_a_forces_5(const T (&D)[56], const T *__restrict__ Ms, T rho, T (&L)[56])
 {
-    L[0] = 0.0f;
-    float rp = 1.0f;
-    { const float m = __ldg(Ms + 0) * rp;
+    L[0] = T(0);
+    T rp = T(1);
+    { const T m = __ldg(Ms + 0) * rp;
       L[1] = D[1] * m;
       L[2] = D[2] * m;
       L[3] = D[3] * m;
@@ -3351,434 +3357,434 @@ __device__ __forceinline__ void m2l_side_a_forces_5(const float (&D)[56], const 
       L[55] = D[55] * m;
     }
     rp *= rho;
-    { const float m = -__ldg(Ms + 1) * rp;
-      L[1] = fmaf(D[4], m, L[1]);
-      L[2] = fmaf(D[5], m, L[2]);
-      L[3] = fmaf(D[6], m, L[3]);
-      L[4] = fmaf(D[10], m, L[4]);
-      L[5] = fmaf(D[11], m, L[5]);
-      L[6] = fmaf(D[12], m, L[6]);
-      L[7] = fmaf(D[13], m, L[7]);
-      L[8] = fmaf(D[14], m, L[8]);
-      L[9] = fmaf(D[15], m, L[9]);
-      L[10] = fmaf(D[20], m, L[10]);
-      L[11] = fmaf(D[21], m, L[11]);
-      L[12] = fmaf(D[22], m, L[12]);
-      L[13] = fmaf(D[23], m, L[13]);
-      L[14] = fmaf(D[24], m, L[14]);
-      L[15] = fmaf(D[25], m, L[15]);
-      L[16] = fmaf(D[26], m, L[16]);
-      L[17] = fmaf(D[27], m, L[17]);
-      L[18] = fmaf(D[28], m, L[18]);
-      L[19] = fmaf(D[29], m, L[19]);
-      L[20] = fmaf(D[35], m, L[20]);
-      L[21] = fmaf(D[36], m, L[21]);
-      L[22] = fmaf(D[37], m, L[22]);
-      L[23] = fmaf(D[38], m, L[23]);
-      L[24] = fmaf(D[39], m, L[24]);
-      L[25] = fmaf(D[40], m, L[25]);
-      L[26] = fmaf(D[41], m, L[26]);
-      L[27] = fmaf(D[42], m, L[27]);
-      L[28] = fmaf(D[43], m, L[28]);
-      L[29] = fmaf(D[44], m, L[29]);
-      L[30] = fmaf(D[45], m, L[30]);
-      L[31] = fmaf(D[46], m, L[31]);
-      L[32] = fmaf(D[47], m, L[32]);
-      L[33] = fmaf(D[48], m, L[33]);
-      L[34] = fmaf(D[49], m, L[34]);
+    { const T m = -__ldg(Ms + 1) * rp;
+      L[1] = m2l_fma(D[4], m, L[1]);
+      L[2] = m2l_fma(D[5], m, L[2]);
+      L[3] = m2l_fma(D[6], m, L[3]);
+      L[4] = m2l_fma(D[10], m, L[4]);
+      L[5] = m2l_fma(D[11], m, L[5]);
+      L[6] = m2l_fma(D[12], m, L[6]);
+      L[7] = m2l_fma(D[13], m, L[7]);
+      L[8] = m2l_fma(D[14], m, L[8]);
+      L[9] = m2l_fma(D[15], m, L[9]);
+      L[10] = m2l_fma(D[20], m, L[10]);
+      L[11] = m2l_fma(D[21], m, L[11]);
+      L[12] = m2l_fma(D[22], m, L[12]);
+      L[13] = m2l_fma(D[23], m, L[13]);
+      L[14] = m2l_fma(D[24], m, L[14]);
+      L[15] = m2l_fma(D[25], m, L[15]);
+      L[16] = m2l_fma(D[26], m, L[16]);
+      L[17] = m2l_fma(D[27], m, L[17]);
+      L[18] = m2l_fma(D[28], m, L[18]);
+      L[19] = m2l_fma(D[29], m, L[19]);
+      L[20] = m2l_fma(D[35], m, L[20]);
+      L[21] = m2l_fma(D[36], m, L[21]);
+      L[22] = m2l_fma(D[37], m, L[22]);
+      L[23] = m2l_fma(D[38], m, L[23]);
+      L[24] = m2l_fma(D[39], m, L[24]);
+      L[25] = m2l_fma(D[40], m, L[25]);
+      L[26] = m2l_fma(D[41], m, L[26]);
+      L[27] = m2l_fma(D[42], m, L[27]);
+      L[28] = m2l_fma(D[43], m, L[28]);
+      L[29] = m2l_fma(D[44], m, L[29]);
+      L[30] = m2l_fma(D[45], m, L[30]);
+      L[31] = m2l_fma(D[46], m, L[31]);
+      L[32] = m2l_fma(D[47], m, L[32]);
+      L[33] = m2l_fma(D[48], m, L[33]);
+      L[34] = m2l_fma(D[49], m, L[34]);
     }
-    { const float m = -__ldg(Ms + 2) * rp;
-      L[1] = fmaf(D[5], m, L[1]);
-      L[2] = fmaf(D[7], m, L[2]);
-      L[3] = fmaf(D[8], m, L[3]);
-      L[4] = fmaf(D[11], m, L[4]);
-      L[5] = fmaf(D[13], m, L[5]);
-      L[6] = fmaf(D[14], m, L[6]);
-      L[7] = fmaf(D[16], m, L[7]);
-      L[8] = fmaf(D[17], m, L[8]);
-      L[9] = fmaf(D[18], m, L[9]);
-      L[10] = fmaf(D[21], m, L[10]);
-      L[11] = fmaf(D[23], m, L[11]);
-      L[12] = fmaf(D[24], m, L[12]);
-      L[13] = fmaf(D[26], m, L[13]);
-      L[14] = fmaf(D[27], m, L[14]);
-      L[15] = fmaf(D[28], m, L[15]);
-      L[16] = fmaf(D[30], m, L[16]);
-      L[17] = fmaf(D[31], m, L[17]);
-      L[18] = fmaf(D[32], m, L[18]);
-      L[19] = fmaf(D[33], m, L[19]);
-      L[20] = fmaf(D[36], m, L[20]);
-      L[21] = fmaf(D[38], m, L[21]);
-      L[22] = fmaf(D[39], m, L[22]);
-      L[23] = fmaf(D[41], m, L[23]);
-      L[24] = fmaf(D[42], m, L[24]);
-      L[25] = fmaf(D[43], m, L[25]);
-      L[26] = fmaf(D[45], m, L[26]);
-      L[27] = fmaf(D[46], m, L[27]);
-      L[28] = fmaf(D[47], m, L[28]);
-      L[29] = fmaf(D[48], m, L[29]);
-      L[30] = fmaf(D[50], m, L[30]);
-      L[31] = fmaf(D[51], m, L[31]);
-      L[32] = fmaf(D[52], m, L[32]);
-      L[33] = fmaf(D[53], m, L[33]);
-      L[34] = fmaf(D[54], m, L[34]);
+    { const T m = -__ldg(Ms + 2) * rp;
+      L[1] = m2l_fma(D[5], m, L[1]);
+      L[2] = m2l_fma(D[7], m, L[2]);
+      L[3] = m2l_fma(D[8], m, L[3]);
+      L[4] = m2l_fma(D[11], m, L[4]);
+      L[5] = m2l_fma(D[13], m, L[5]);
+      L[6] = m2l_fma(D[14], m, L[6]);
+      L[7] = m2l_fma(D[16], m, L[7]);
+      L[8] = m2l_fma(D[17], m, L[8]);
+      L[9] = m2l_fma(D[18], m, L[9]);
+      L[10] = m2l_fma(D[21], m, L[10]);
+      L[11] = m2l_fma(D[23], m, L[11]);
+      L[12] = m2l_fma(D[24], m, L[12]);
+      L[13] = m2l_fma(D[26], m, L[13]);
+      L[14] = m2l_fma(D[27], m, L[14]);
+      L[15] = m2l_fma(D[28], m, L[15]);
+      L[16] = m2l_fma(D[30], m, L[16]);
+      L[17] = m2l_fma(D[31], m, L[17]);
+      L[18] = m2l_fma(D[32], m, L[18]);
+      L[19] = m2l_fma(D[33], m, L[19]);
+      L[20] = m2l_fma(D[36], m, L[20]);
+      L[21] = m2l_fma(D[38], m, L[21]);
+      L[22] = m2l_fma(D[39], m, L[22]);
+      L[23] = m2l_fma(D[41], m, L[23]);
+      L[24] = m2l_fma(D[42], m, L[24]);
+      L[25] = m2l_fma(D[43], m, L[25]);
+      L[26] = m2l_fma(D[45], m, L[26]);
+      L[27] = m2l_fma(D[46], m, L[27]);
+      L[28] = m2l_fma(D[47], m, L[28]);
+      L[29] = m2l_fma(D[48], m, L[29]);
+      L[30] = m2l_fma(D[50], m, L[30]);
+      L[31] = m2l_fma(D[51], m, L[31]);
+      L[32] = m2l_fma(D[52], m, L[32]);
+      L[33] = m2l_fma(D[53], m, L[33]);
+      L[34] = m2l_fma(D[54], m, L[34]);
     }
-    { const float m = -__ldg(Ms + 3) * rp;
-      L[1] = fmaf(D[6], m, L[1]);
-      L[2] = fmaf(D[8], m, L[2]);
-      L[3] = fmaf(D[9], m, L[3]);
-      L[4] = fmaf(D[12], m, L[4]);
-      L[5] = fmaf(D[14], m, L[5]);
-      L[6] = fmaf(D[15], m, L[6]);
-      L[7] = fmaf(D[17], m, L[7]);
-      L[8] = fmaf(D[18], m, L[8]);
-      L[9] = fmaf(D[19], m, L[9]);
-      L[10] = fmaf(D[22], m, L[10]);
-      L[11] = fmaf(D[24], m, L[11]);
-      L[12] = fmaf(D[25], m, L[12]);
-      L[13] = fmaf(D[27], m, L[13]);
-      L[14] = fmaf(D[28], m, L[14]);
-      L[15] = fmaf(D[29], m, L[15]);
-      L[16] = fmaf(D[31], m, L[16]);
-      L[17] = fmaf(D[32], m, L[17]);
-      L[18] = fmaf(D[33], m, L[18]);
-      L[19] = fmaf(D[34], m, L[19]);
-      L[20] = fmaf(D[37], m, L[20]);
-      L[21] = fmaf(D[39], m, L[21]);
-      L[22] = fmaf(D[40], m, L[22]);
-      L[23] = fmaf(D[42], m, L[23]);
-      L[24] = fmaf(D[43], m, L[24]);
-      L[25] = fmaf(D[44], m, L[25]);
-      L[26] = fmaf(D[46], m, L[26]);
-      L[27] = fmaf(D[47], m, L[27]);
-      L[28] = fmaf(D[48], m, L[28]);
-      L[29] = fmaf(D[49], m, L[29]);
-      L[30] = fmaf(D[51], m, L[30]);
-      L[31] = fmaf(D[52], m, L[31]);
-      L[32] = fmaf(D[53], m, L[32]);
-      L[33] = fmaf(D[54], m, L[33]);
-      L[34] = fmaf(D[55], m, L[34]);
-    }
-    rp *= rho;
-    { const float m = __ldg(Ms + 4) * rp;
-      L[1] = fmaf(D[10], m, L[1]);
-      L[2] = fmaf(D[11], m, L[2]);
-      L[3] = fmaf(D[12], m, L[3]);
-      L[4] = fmaf(D[20], m, L[4]);
-      L[5] = fmaf(D[21], m, L[5]);
-      L[6] = fmaf(D[22], m, L[6]);
-      L[7] = fmaf(D[23], m, L[7]);
-      L[8] = fmaf(D[24], m, L[8]);
-      L[9] = fmaf(D[25], m, L[9]);
-      L[10] = fmaf(D[35], m, L[10]);
-      L[11] = fmaf(D[36], m, L[11]);
-      L[12] = fmaf(D[37], m, L[12]);
-      L[13] = fmaf(D[38], m, L[13]);
-      L[14] = fmaf(D[39], m, L[14]);
-      L[15] = fmaf(D[40], m, L[15]);
-      L[16] = fmaf(D[41], m, L[16]);
-      L[17] = fmaf(D[42], m, L[17]);
-      L[18] = fmaf(D[43], m, L[18]);
-      L[19] = fmaf(D[44], m, L[19]);
-    }
-    { const float m = __ldg(Ms + 5) * rp;
-      L[1] = fmaf(D[11], m, L[1]);
-      L[2] = fmaf(D[13], m, L[2]);
-      L[3] = fmaf(D[14], m, L[3]);
-      L[4] = fmaf(D[21], m, L[4]);
-      L[5] = fmaf(D[23], m, L[5]);
-      L[6] = fmaf(D[24], m, L[6]);
-      L[7] = fmaf(D[26], m, L[7]);
-      L[8] = fmaf(D[27], m, L[8]);
-      L[9] = fmaf(D[28], m, L[9]);
-      L[10] = fmaf(D[36], m, L[10]);
-      L[11] = fmaf(D[38], m, L[11]);
-      L[12] = fmaf(D[39], m, L[12]);
-      L[13] = fmaf(D[41], m, L[13]);
-      L[14] = fmaf(D[42], m, L[14]);
-      L[15] = fmaf(D[43], m, L[15]);
-      L[16] = fmaf(D[45], m, L[16]);
-      L[17] = fmaf(D[46], m, L[17]);
-      L[18] = fmaf(D[47], m, L[18]);
-      L[19] = fmaf(D[48], m, L[19]);
-    }
-    { const float m = __ldg(Ms + 6) * rp;
-      L[1] = fmaf(D[12], m, L[1]);
-      L[2] = fmaf(D[14], m, L[2]);
-      L[3] = fmaf(D[15], m, L[3]);
-      L[4] = fmaf(D[22], m, L[4]);
-      L[5] = fmaf(D[24], m, L[5]);
-      L[6] = fmaf(D[25], m, L[6]);
-      L[7] = fmaf(D[27], m, L[7]);
-      L[8] = fmaf(D[28], m, L[8]);
-      L[9] = fmaf(D[29], m, L[9]);
-      L[10] = fmaf(D[37], m, L[10]);
-      L[11] = fmaf(D[39], m, L[11]);
-      L[12] = fmaf(D[40], m, L[12]);
-      L[13] = fmaf(D[42], m, L[13]);
-      L[14] = fmaf(D[43], m, L[14]);
-      L[15] = fmaf(D[44], m, L[15]);
-      L[16] = fmaf(D[46], m, L[16]);
-      L[17] = fmaf(D[47], m, L[17]);
-      L[18] = fmaf(D[48], m, L[18]);
-      L[19] = fmaf(D[49], m, L[19]);
-    }
-    { const float m = __ldg(Ms + 7) * rp;
-      L[1] = fmaf(D[13], m, L[1]);
-      L[2] = fmaf(D[16], m, L[2]);
-      L[3] = fmaf(D[17], m, L[3]);
-      L[4] = fmaf(D[23], m, L[4]);
-      L[5] = fmaf(D[26], m, L[5]);
-      L[6] = fmaf(D[27], m, L[6]);
-      L[7] = fmaf(D[30], m, L[7]);
-      L[8] = fmaf(D[31], m, L[8]);
-      L[9] = fmaf(D[32], m, L[9]);
-      L[10] = fmaf(D[38], m, L[10]);
-      L[11] = fmaf(D[41], m, L[11]);
-      L[12] = fmaf(D[42], m, L[12]);
-      L[13] = fmaf(D[45], m, L[13]);
-      L[14] = fmaf(D[46], m, L[14]);
-      L[15] = fmaf(D[47], m, L[15]);
-      L[16] = fmaf(D[50], m, L[16]);
-      L[17] = fmaf(D[51], m, L[17]);
-      L[18] = fmaf(D[52], m, L[18]);
-      L[19] = fmaf(D[53], m, L[19]);
-    }
-    { const float m = __ldg(Ms + 8) * rp;
-      L[1] = fmaf(D[14], m, L[1]);
-      L[2] = fmaf(D[17], m, L[2]);
-      L[3] = fmaf(D[18], m, L[3]);
-      L[4] = fmaf(D[24], m, L[4]);
-      L[5] = fmaf(D[27], m, L[5]);
-      L[6] = fmaf(D[28], m, L[6]);
-      L[7] = fmaf(D[31], m, L[7]);
-      L[8] = fmaf(D[32], m, L[8]);
-      L[9] = fmaf(D[33], m, L[9]);
-      L[10] = fmaf(D[39], m, L[10]);
-      L[11] = fmaf(D[42], m, L[11]);
-      L[12] = fmaf(D[43], m, L[12]);
-      L[13] = fmaf(D[46], m, L[13]);
-      L[14] = fmaf(D[47], m, L[14]);
-      L[15] = fmaf(D[48], m, L[15]);
-      L[16] = fmaf(D[51], m, L[16]);
-      L[17] = fmaf(D[52], m, L[17]);
-      L[18] = fmaf(D[53], m, L[18]);
-      L[19] = fmaf(D[54], m, L[19]);
-    }
-    { const float m = __ldg(Ms + 9) * rp;
-      L[1] = fmaf(D[15], m, L[1]);
-      L[2] = fmaf(D[18], m, L[2]);
-      L[3] = fmaf(D[19], m, L[3]);
-      L[4] = fmaf(D[25], m, L[4]);
-      L[5] = fmaf(D[28], m, L[5]);
-      L[6] = fmaf(D[29], m, L[6]);
-      L[7] = fmaf(D[32], m, L[7]);
-      L[8] = fmaf(D[33], m, L[8]);
-      L[9] = fmaf(D[34], m, L[9]);
-      L[10] = fmaf(D[40], m, L[10]);
-      L[11] = fmaf(D[43], m, L[11]);
-      L[12] = fmaf(D[44], m, L[12]);
-      L[13] = fmaf(D[47], m, L[13]);
-      L[14] = fmaf(D[48], m, L[14]);
-      L[15] = fmaf(D[49], m, L[15]);
-      L[16] = fmaf(D[52], m, L[16]);
-      L[17] = fmaf(D[53], m, L[17]);
-      L[18] = fmaf(D[54], m, L[18]);
-      L[19] = fmaf(D[55], m, L[19]);
+    { const T m = -__ldg(Ms + 3) * rp;
+      L[1] = m2l_fma(D[6], m, L[1]);
+      L[2] = m2l_fma(D[8], m, L[2]);
+      L[3] = m2l_fma(D[9], m, L[3]);
+      L[4] = m2l_fma(D[12], m, L[4]);
+      L[5] = m2l_fma(D[14], m, L[5]);
+      L[6] = m2l_fma(D[15], m, L[6]);
+      L[7] = m2l_fma(D[17], m, L[7]);
+      L[8] = m2l_fma(D[18], m, L[8]);
+      L[9] = m2l_fma(D[19], m, L[9]);
+      L[10] = m2l_fma(D[22], m, L[10]);
+      L[11] = m2l_fma(D[24], m, L[11]);
+      L[12] = m2l_fma(D[25], m, L[12]);
+      L[13] = m2l_fma(D[27], m, L[13]);
+      L[14] = m2l_fma(D[28], m, L[14]);
+      L[15] = m2l_fma(D[29], m, L[15]);
+      L[16] = m2l_fma(D[31], m, L[16]);
+      L[17] = m2l_fma(D[32], m, L[17]);
+      L[18] = m2l_fma(D[33], m, L[18]);
+      L[19] = m2l_fma(D[34], m, L[19]);
+      L[20] = m2l_fma(D[37], m, L[20]);
+      L[21] = m2l_fma(D[39], m, L[21]);
+      L[22] = m2l_fma(D[40], m, L[22]);
+      L[23] = m2l_fma(D[42], m, L[23]);
+      L[24] = m2l_fma(D[43], m, L[24]);
+      L[25] = m2l_fma(D[44], m, L[25]);
+      L[26] = m2l_fma(D[46], m, L[26]);
+      L[27] = m2l_fma(D[47], m, L[27]);
+      L[28] = m2l_fma(D[48], m, L[28]);
+      L[29] = m2l_fma(D[49], m, L[29]);
+      L[30] = m2l_fma(D[51], m, L[30]);
+      L[31] = m2l_fma(D[52], m, L[31]);
+      L[32] = m2l_fma(D[53], m, L[32]);
+      L[33] = m2l_fma(D[54], m, L[33]);
+      L[34] = m2l_fma(D[55], m, L[34]);
     }
     rp *= rho;
-    { const float m = -__ldg(Ms + 10) * rp;
-      L[1] = fmaf(D[20], m, L[1]);
-      L[2] = fmaf(D[21], m, L[2]);
-      L[3] = fmaf(D[22], m, L[3]);
-      L[4] = fmaf(D[35], m, L[4]);
-      L[5] = fmaf(D[36], m, L[5]);
-      L[6] = fmaf(D[37], m, L[6]);
-      L[7] = fmaf(D[38], m, L[7]);
-      L[8] = fmaf(D[39], m, L[8]);
-      L[9] = fmaf(D[40], m, L[9]);
+    { const T m = __ldg(Ms + 4) * rp;
+      L[1] = m2l_fma(D[10], m, L[1]);
+      L[2] = m2l_fma(D[11], m, L[2]);
+      L[3] = m2l_fma(D[12], m, L[3]);
+      L[4] = m2l_fma(D[20], m, L[4]);
+      L[5] = m2l_fma(D[21], m, L[5]);
+      L[6] = m2l_fma(D[22], m, L[6]);
+      L[7] = m2l_fma(D[23], m, L[7]);
+      L[8] = m2l_fma(D[24], m, L[8]);
+      L[9] = m2l_fma(D[25], m, L[9]);
+      L[10] = m2l_fma(D[35], m, L[10]);
+      L[11] = m2l_fma(D[36], m, L[11]);
+      L[12] = m2l_fma(D[37], m, L[12]);
+      L[13] = m2l_fma(D[38], m, L[13]);
+      L[14] = m2l_fma(D[39], m, L[14]);
+      L[15] = m2l_fma(D[40], m, L[15]);
+      L[16] = m2l_fma(D[41], m, L[16]);
+      L[17] = m2l_fma(D[42], m, L[17]);
+      L[18] = m2l_fma(D[43], m, L[18]);
+      L[19] = m2l_fma(D[44], m, L[19]);
     }
-    { const float m = -__ldg(Ms + 11) * rp;
-      L[1] = fmaf(D[21], m, L[1]);
-      L[2] = fmaf(D[23], m, L[2]);
-      L[3] = fmaf(D[24], m, L[3]);
-      L[4] = fmaf(D[36], m, L[4]);
-      L[5] = fmaf(D[38], m, L[5]);
-      L[6] = fmaf(D[39], m, L[6]);
-      L[7] = fmaf(D[41], m, L[7]);
-      L[8] = fmaf(D[42], m, L[8]);
-      L[9] = fmaf(D[43], m, L[9]);
+    { const T m = __ldg(Ms + 5) * rp;
+      L[1] = m2l_fma(D[11], m, L[1]);
+      L[2] = m2l_fma(D[13], m, L[2]);
+      L[3] = m2l_fma(D[14], m, L[3]);
+      L[4] = m2l_fma(D[21], m, L[4]);
+      L[5] = m2l_fma(D[23], m, L[5]);
+      L[6] = m2l_fma(D[24], m, L[6]);
+      L[7] = m2l_fma(D[26], m, L[7]);
+      L[8] = m2l_fma(D[27], m, L[8]);
+      L[9] = m2l_fma(D[28], m, L[9]);
+      L[10] = m2l_fma(D[36], m, L[10]);
+      L[11] = m2l_fma(D[38], m, L[11]);
+      L[12] = m2l_fma(D[39], m, L[12]);
+      L[13] = m2l_fma(D[41], m, L[13]);
+      L[14] = m2l_fma(D[42], m, L[14]);
+      L[15] = m2l_fma(D[43], m, L[15]);
+      L[16] = m2l_fma(D[45], m, L[16]);
+      L[17] = m2l_fma(D[46], m, L[17]);
+      L[18] = m2l_fma(D[47], m, L[18]);
+      L[19] = m2l_fma(D[48], m, L[19]);
     }
-    { const float m = -__ldg(Ms + 12) * rp;
-      L[1] = fmaf(D[22], m, L[1]);
-      L[2] = fmaf(D[24], m, L[2]);
-      L[3] = fmaf(D[25], m, L[3]);
-      L[4] = fmaf(D[37], m, L[4]);
-      L[5] = fmaf(D[39], m, L[5]);
-      L[6] = fmaf(D[40], m, L[6]);
-      L[7] = fmaf(D[42], m, L[7]);
-      L[8] = fmaf(D[43], m, L[8]);
-      L[9] = fmaf(D[44], m, L[9]);
+    { const T m = __ldg(Ms + 6) * rp;
+      L[1] = m2l_fma(D[12], m, L[1]);
+      L[2] = m2l_fma(D[14], m, L[2]);
+      L[3] = m2l_fma(D[15], m, L[3]);
+      L[4] = m2l_fma(D[22], m, L[4]);
+      L[5] = m2l_fma(D[24], m, L[5]);
+      L[6] = m2l_fma(D[25], m, L[6]);
+      L[7] = m2l_fma(D[27], m, L[7]);
+      L[8] = m2l_fma(D[28], m, L[8]);
+      L[9] = m2l_fma(D[29], m, L[9]);
+      L[10] = m2l_fma(D[37], m, L[10]);
+      L[11] = m2l_fma(D[39], m, L[11]);
+      L[12] = m2l_fma(D[40], m, L[12]);
+      L[13] = m2l_fma(D[42], m, L[13]);
+      L[14] = m2l_fma(D[43], m, L[14]);
+      L[15] = m2l_fma(D[44], m, L[15]);
+      L[16] = m2l_fma(D[46], m, L[16]);
+      L[17] = m2l_fma(D[47], m, L[17]);
+      L[18] = m2l_fma(D[48], m, L[18]);
+      L[19] = m2l_fma(D[49], m, L[19]);
     }
-    { const float m = -__ldg(Ms + 13) * rp;
-      L[1] = fmaf(D[23], m, L[1]);
-      L[2] = fmaf(D[26], m, L[2]);
-      L[3] = fmaf(D[27], m, L[3]);
-      L[4] = fmaf(D[38], m, L[4]);
-      L[5] = fmaf(D[41], m, L[5]);
-      L[6] = fmaf(D[42], m, L[6]);
-      L[7] = fmaf(D[45], m, L[7]);
-      L[8] = fmaf(D[46], m, L[8]);
-      L[9] = fmaf(D[47], m, L[9]);
+    { const T m = __ldg(Ms + 7) * rp;
+      L[1] = m2l_fma(D[13], m, L[1]);
+      L[2] = m2l_fma(D[16], m, L[2]);
+      L[3] = m2l_fma(D[17], m, L[3]);
+      L[4] = m2l_fma(D[23], m, L[4]);
+      L[5] = m2l_fma(D[26], m, L[5]);
+      L[6] = m2l_fma(D[27], m, L[6]);
+      L[7] = m2l_fma(D[30], m, L[7]);
+      L[8] = m2l_fma(D[31], m, L[8]);
+      L[9] = m2l_fma(D[32], m, L[9]);
+      L[10] = m2l_fma(D[38], m, L[10]);
+      L[11] = m2l_fma(D[41], m, L[11]);
+      L[12] = m2l_fma(D[42], m, L[12]);
+      L[13] = m2l_fma(D[45], m, L[13]);
+      L[14] = m2l_fma(D[46], m, L[14]);
+      L[15] = m2l_fma(D[47], m, L[15]);
+      L[16] = m2l_fma(D[50], m, L[16]);
+      L[17] = m2l_fma(D[51], m, L[17]);
+      L[18] = m2l_fma(D[52], m, L[18]);
+      L[19] = m2l_fma(D[53], m, L[19]);
     }
-    { const float m = -__ldg(Ms + 14) * rp;
-      L[1] = fmaf(D[24], m, L[1]);
-      L[2] = fmaf(D[27], m, L[2]);
-      L[3] = fmaf(D[28], m, L[3]);
-      L[4] = fmaf(D[39], m, L[4]);
-      L[5] = fmaf(D[42], m, L[5]);
-      L[6] = fmaf(D[43], m, L[6]);
-      L[7] = fmaf(D[46], m, L[7]);
-      L[8] = fmaf(D[47], m, L[8]);
-      L[9] = fmaf(D[48], m, L[9]);
+    { const T m = __ldg(Ms + 8) * rp;
+      L[1] = m2l_fma(D[14], m, L[1]);
+      L[2] = m2l_fma(D[17], m, L[2]);
+      L[3] = m2l_fma(D[18], m, L[3]);
+      L[4] = m2l_fma(D[24], m, L[4]);
+      L[5] = m2l_fma(D[27], m, L[5]);
+      L[6] = m2l_fma(D[28], m, L[6]);
+      L[7] = m2l_fma(D[31], m, L[7]);
+      L[8] = m2l_fma(D[32], m, L[8]);
+      L[9] = m2l_fma(D[33], m, L[9]);
+      L[10] = m2l_fma(D[39], m, L[10]);
+      L[11] = m2l_fma(D[42], m, L[11]);
+      L[12] = m2l_fma(D[43], m, L[12]);
+      L[13] = m2l_fma(D[46], m, L[13]);
+      L[14] = m2l_fma(D[47], m, L[14]);
+      L[15] = m2l_fma(D[48], m, L[15]);
+      L[16] = m2l_fma(D[51], m, L[16]);
+      L[17] = m2l_fma(D[52], m, L[17]);
+      L[18] = m2l_fma(D[53], m, L[18]);
+      L[19] = m2l_fma(D[54], m, L[19]);
     }
-    { const float m = -__ldg(Ms + 15) * rp;
-      L[1] = fmaf(D[25], m, L[1]);
-      L[2] = fmaf(D[28], m, L[2]);
-      L[3] = fmaf(D[29], m, L[3]);
-      L[4] = fmaf(D[40], m, L[4]);
-      L[5] = fmaf(D[43], m, L[5]);
-      L[6] = fmaf(D[44], m, L[6]);
-      L[7] = fmaf(D[47], m, L[7]);
-      L[8] = fmaf(D[48], m, L[8]);
-      L[9] = fmaf(D[49], m, L[9]);
-    }
-    { const float m = -__ldg(Ms + 16) * rp;
-      L[1] = fmaf(D[26], m, L[1]);
-      L[2] = fmaf(D[30], m, L[2]);
-      L[3] = fmaf(D[31], m, L[3]);
-      L[4] = fmaf(D[41], m, L[4]);
-      L[5] = fmaf(D[45], m, L[5]);
-      L[6] = fmaf(D[46], m, L[6]);
-      L[7] = fmaf(D[50], m, L[7]);
-      L[8] = fmaf(D[51], m, L[8]);
-      L[9] = fmaf(D[52], m, L[9]);
-    }
-    { const float m = -__ldg(Ms + 17) * rp;
-      L[1] = fmaf(D[27], m, L[1]);
-      L[2] = fmaf(D[31], m, L[2]);
-      L[3] = fmaf(D[32], m, L[3]);
-      L[4] = fmaf(D[42], m, L[4]);
-      L[5] = fmaf(D[46], m, L[5]);
-      L[6] = fmaf(D[47], m, L[6]);
-      L[7] = fmaf(D[51], m, L[7]);
-      L[8] = fmaf(D[52], m, L[8]);
-      L[9] = fmaf(D[53], m, L[9]);
-    }
-    { const float m = -__ldg(Ms + 18) * rp;
-      L[1] = fmaf(D[28], m, L[1]);
-      L[2] = fmaf(D[32], m, L[2]);
-      L[3] = fmaf(D[33], m, L[3]);
-      L[4] = fmaf(D[43], m, L[4]);
-      L[5] = fmaf(D[47], m, L[5]);
-      L[6] = fmaf(D[48], m, L[6]);
-      L[7] = fmaf(D[52], m, L[7]);
-      L[8] = fmaf(D[53], m, L[8]);
-      L[9] = fmaf(D[54], m, L[9]);
-    }
-    { const float m = -__ldg(Ms + 19) * rp;
-      L[1] = fmaf(D[29], m, L[1]);
-      L[2] = fmaf(D[33], m, L[2]);
-      L[3] = fmaf(D[34], m, L[3]);
-      L[4] = fmaf(D[44], m, L[4]);
-      L[5] = fmaf(D[48], m, L[5]);
-      L[6] = fmaf(D[49], m, L[6]);
-      L[7] = fmaf(D[53], m, L[7]);
-      L[8] = fmaf(D[54], m, L[8]);
-      L[9] = fmaf(D[55], m, L[9]);
+    { const T m = __ldg(Ms + 9) * rp;
+      L[1] = m2l_fma(D[15], m, L[1]);
+      L[2] = m2l_fma(D[18], m, L[2]);
+      L[3] = m2l_fma(D[19], m, L[3]);
+      L[4] = m2l_fma(D[25], m, L[4]);
+      L[5] = m2l_fma(D[28], m, L[5]);
+      L[6] = m2l_fma(D[29], m, L[6]);
+      L[7] = m2l_fma(D[32], m, L[7]);
+      L[8] = m2l_fma(D[33], m, L[8]);
+      L[9] = m2l_fma(D[34], m, L[9]);
+      L[10] = m2l_fma(D[40], m, L[10]);
+      L[11] = m2l_fma(D[43], m, L[11]);
+      L[12] = m2l_fma(D[44], m, L[12]);
+      L[13] = m2l_fma(D[47], m, L[13]);
+      L[14] = m2l_fma(D[48], m, L[14]);
+      L[15] = m2l_fma(D[49], m, L[15]);
+      L[16] = m2l_fma(D[52], m, L[16]);
+      L[17] = m2l_fma(D[53], m, L[17]);
+      L[18] = m2l_fma(D[54], m, L[18]);
+      L[19] = m2l_fma(D[55], m, L[19]);
     }
     rp *= rho;
-    { const float m = __ldg(Ms + 20) * rp;
-      L[1] = fmaf(D[35], m, L[1]);
-      L[2] = fmaf(D[36], m, L[2]);
-      L[3] = fmaf(D[37], m, L[3]);
+    { const T m = -__ldg(Ms + 10) * rp;
+      L[1] = m2l_fma(D[20], m, L[1]);
+      L[2] = m2l_fma(D[21], m, L[2]);
+      L[3] = m2l_fma(D[22], m, L[3]);
+      L[4] = m2l_fma(D[35], m, L[4]);
+      L[5] = m2l_fma(D[36], m, L[5]);
+      L[6] = m2l_fma(D[37], m, L[6]);
+      L[7] = m2l_fma(D[38], m, L[7]);
+      L[8] = m2l_fma(D[39], m, L[8]);
+      L[9] = m2l_fma(D[40], m, L[9]);
     }
-    { const float m = __ldg(Ms + 21) * rp;
-      L[1] = fmaf(D[36], m, L[1]);
-      L[2] = fmaf(D[38], m, L[2]);
-      L[3] = fmaf(D[39], m, L[3]);
+    { const T m = -__ldg(Ms + 11) * rp;
+      L[1] = m2l_fma(D[21], m, L[1]);
+      L[2] = m2l_fma(D[23], m, L[2]);
+      L[3] = m2l_fma(D[24], m, L[3]);
+      L[4] = m2l_fma(D[36], m, L[4]);
+      L[5] = m2l_fma(D[38], m, L[5]);
+      L[6] = m2l_fma(D[39], m, L[6]);
+      L[7] = m2l_fma(D[41], m, L[7]);
+      L[8] = m2l_fma(D[42], m, L[8]);
+      L[9] = m2l_fma(D[43], m, L[9]);
     }
-    { const float m = __ldg(Ms + 22) * rp;
-      L[1] = fmaf(D[37], m, L[1]);
-      L[2] = fmaf(D[39], m, L[2]);
-      L[3] = fmaf(D[40], m, L[3]);
+    { const T m = -__ldg(Ms + 12) * rp;
+      L[1] = m2l_fma(D[22], m, L[1]);
+      L[2] = m2l_fma(D[24], m, L[2]);
+      L[3] = m2l_fma(D[25], m, L[3]);
+      L[4] = m2l_fma(D[37], m, L[4]);
+      L[5] = m2l_fma(D[39], m, L[5]);
+      L[6] = m2l_fma(D[40], m, L[6]);
+      L[7] = m2l_fma(D[42], m, L[7]);
+      L[8] = m2l_fma(D[43], m, L[8]);
+      L[9] = m2l_fma(D[44], m, L[9]);
     }
-    { const float m = __ldg(Ms + 23) * rp;
-      L[1] = fmaf(D[38], m, L[1]);
-      L[2] = fmaf(D[41], m, L[2]);
-      L[3] = fmaf(D[42], m, L[3]);
+    { const T m = -__ldg(Ms + 13) * rp;
+      L[1] = m2l_fma(D[23], m, L[1]);
+      L[2] = m2l_fma(D[26], m, L[2]);
+      L[3] = m2l_fma(D[27], m, L[3]);
+      L[4] = m2l_fma(D[38], m, L[4]);
+      L[5] = m2l_fma(D[41], m, L[5]);
+      L[6] = m2l_fma(D[42], m, L[6]);
+      L[7] = m2l_fma(D[45], m, L[7]);
+      L[8] = m2l_fma(D[46], m, L[8]);
+      L[9] = m2l_fma(D[47], m, L[9]);
     }
-    { const float m = __ldg(Ms + 24) * rp;
-      L[1] = fmaf(D[39], m, L[1]);
-      L[2] = fmaf(D[42], m, L[2]);
-      L[3] = fmaf(D[43], m, L[3]);
+    { const T m = -__ldg(Ms + 14) * rp;
+      L[1] = m2l_fma(D[24], m, L[1]);
+      L[2] = m2l_fma(D[27], m, L[2]);
+      L[3] = m2l_fma(D[28], m, L[3]);
+      L[4] = m2l_fma(D[39], m, L[4]);
+      L[5] = m2l_fma(D[42], m, L[5]);
+      L[6] = m2l_fma(D[43], m, L[6]);
+      L[7] = m2l_fma(D[46], m, L[7]);
+      L[8] = m2l_fma(D[47], m, L[8]);
+      L[9] = m2l_fma(D[48], m, L[9]);
     }
-    { const float m = __ldg(Ms + 25) * rp;
-      L[1] = fmaf(D[40], m, L[1]);
-      L[2] = fmaf(D[43], m, L[2]);
-      L[3] = fmaf(D[44], m, L[3]);
+    { const T m = -__ldg(Ms + 15) * rp;
+      L[1] = m2l_fma(D[25], m, L[1]);
+      L[2] = m2l_fma(D[28], m, L[2]);
+      L[3] = m2l_fma(D[29], m, L[3]);
+      L[4] = m2l_fma(D[40], m, L[4]);
+      L[5] = m2l_fma(D[43], m, L[5]);
+      L[6] = m2l_fma(D[44], m, L[6]);
+      L[7] = m2l_fma(D[47], m, L[7]);
+      L[8] = m2l_fma(D[48], m, L[8]);
+      L[9] = m2l_fma(D[49], m, L[9]);
     }
-    { const float m = __ldg(Ms + 26) * rp;
-      L[1] = fmaf(D[41], m, L[1]);
-      L[2] = fmaf(D[45], m, L[2]);
-      L[3] = fmaf(D[46], m, L[3]);
+    { const T m = -__ldg(Ms + 16) * rp;
+      L[1] = m2l_fma(D[26], m, L[1]);
+      L[2] = m2l_fma(D[30], m, L[2]);
+      L[3] = m2l_fma(D[31], m, L[3]);
+      L[4] = m2l_fma(D[41], m, L[4]);
+      L[5] = m2l_fma(D[45], m, L[5]);
+      L[6] = m2l_fma(D[46], m, L[6]);
+      L[7] = m2l_fma(D[50], m, L[7]);
+      L[8] = m2l_fma(D[51], m, L[8]);
+      L[9] = m2l_fma(D[52], m, L[9]);
     }
-    { const float m = __ldg(Ms + 27) * rp;
-      L[1] = fmaf(D[42], m, L[1]);
-      L[2] = fmaf(D[46], m, L[2]);
-      L[3] = fmaf(D[47], m, L[3]);
+    { const T m = -__ldg(Ms + 17) * rp;
+      L[1] = m2l_fma(D[27], m, L[1]);
+      L[2] = m2l_fma(D[31], m, L[2]);
+      L[3] = m2l_fma(D[32], m, L[3]);
+      L[4] = m2l_fma(D[42], m, L[4]);
+      L[5] = m2l_fma(D[46], m, L[5]);
+      L[6] = m2l_fma(D[47], m, L[6]);
+      L[7] = m2l_fma(D[51], m, L[7]);
+      L[8] = m2l_fma(D[52], m, L[8]);
+      L[9] = m2l_fma(D[53], m, L[9]);
     }
-    { const float m = __ldg(Ms + 28) * rp;
-      L[1] = fmaf(D[43], m, L[1]);
-      L[2] = fmaf(D[47], m, L[2]);
-      L[3] = fmaf(D[48], m, L[3]);
+    { const T m = -__ldg(Ms + 18) * rp;
+      L[1] = m2l_fma(D[28], m, L[1]);
+      L[2] = m2l_fma(D[32], m, L[2]);
+      L[3] = m2l_fma(D[33], m, L[3]);
+      L[4] = m2l_fma(D[43], m, L[4]);
+      L[5] = m2l_fma(D[47], m, L[5]);
+      L[6] = m2l_fma(D[48], m, L[6]);
+      L[7] = m2l_fma(D[52], m, L[7]);
+      L[8] = m2l_fma(D[53], m, L[8]);
+      L[9] = m2l_fma(D[54], m, L[9]);
     }
-    { const float m = __ldg(Ms + 29) * rp;
-      L[1] = fmaf(D[44], m, L[1]);
-      L[2] = fmaf(D[48], m, L[2]);
-      L[3] = fmaf(D[49], m, L[3]);
+    { const T m = -__ldg(Ms + 19) * rp;
+      L[1] = m2l_fma(D[29], m, L[1]);
+      L[2] = m2l_fma(D[33], m, L[2]);
+      L[3] = m2l_fma(D[34], m, L[3]);
+      L[4] = m2l_fma(D[44], m, L[4]);
+      L[5] = m2l_fma(D[48], m, L[5]);
+      L[6] = m2l_fma(D[49], m, L[6]);
+      L[7] = m2l_fma(D[53], m, L[7]);
+      L[8] = m2l_fma(D[54], m, L[8]);
+      L[9] = m2l_fma(D[55], m, L[9]);
     }
-    { const float m = __ldg(Ms + 30) * rp;
-      L[1] = fmaf(D[45], m, L[1]);
-      L[2] = fmaf(D[50], m, L[2]);
-      L[3] = fmaf(D[51], m, L[3]);
+    rp *= rho;
+    { const T m = __ldg(Ms + 20) * rp;
+      L[1] = m2l_fma(D[35], m, L[1]);
+      L[2] = m2l_fma(D[36], m, L[2]);
+      L[3] = m2l_fma(D[37], m, L[3]);
     }
-    { const float m = __ldg(Ms + 31) * rp;
-      L[1] = fmaf(D[46], m, L[1]);
-      L[2] = fmaf(D[51], m, L[2]);
-      L[3] = fmaf(D[52], m, L[3]);
+    { const T m = __ldg(Ms + 21) * rp;
+      L[1] = m2l_fma(D[36], m, L[1]);
+      L[2] = m2l_fma(D[38], m, L[2]);
+      L[3] = m2l_fma(D[39], m, L[3]);
     }
-    { const float m = __ldg(Ms + 32) * rp;
-      L[1] = fmaf(D[47], m, L[1]);
-      L[2] = fmaf(D[52], m, L[2]);
-      L[3] = fmaf(D[53], m, L[3]);
+    { const T m = __ldg(Ms + 22) * rp;
+      L[1] = m2l_fma(D[37], m, L[1]);
+      L[2] = m2l_fma(D[39], m, L[2]);
+      L[3] = m2l_fma(D[40], m, L[3]);
     }
-    { const float m = __ldg(Ms + 33) * rp;
-      L[1] = fmaf(D[48], m, L[1]);
-      L[2] = fmaf(D[53], m, L[2]);
-      L[3] = fmaf(D[54], m, L[3]);
+    { const T m = __ldg(Ms + 23) * rp;
+      L[1] = m2l_fma(D[38], m, L[1]);
+      L[2] = m2l_fma(D[41], m, L[2]);
+      L[3] = m2l_fma(D[42], m, L[3]);
     }
-    { const float m = __ldg(Ms + 34) * rp;
-      L[1] = fmaf(D[49], m, L[1]);
-      L[2] = fmaf(D[54], m, L[2]);
-      L[3] = fmaf(D[55], m, L[3]);
+    { const T m = __ldg(Ms + 24) * rp;
+      L[1] = m2l_fma(D[39], m, L[1]);
+      L[2] = m2l_fma(D[42], m, L[2]);
+      L[3] = m2l_fma(D[43], m, L[3]);
+    }
+    { const T m = __ldg(Ms + 25) * rp;
+      L[1] = m2l_fma(D[40], m, L[1]);
+      L[2] = m2l_fma(D[43], m, L[2]);
+      L[3] = m2l_fma(D[44], m, L[3]);
+    }
+    { const T m = __ldg(Ms + 26) * rp;
+      L[1] = m2l_fma(D[41], m, L[1]);
+      L[2] = m2l_fma(D[45], m, L[2]);
+      L[3] = m2l_fma(D[46], m, L[3]);
+    }
+    { const T m = __ldg(Ms + 27) * rp;
+      L[1] = m2l_fma(D[42], m, L[1]);
+      L[2] = m2l_fma(D[46], m, L[2]);
+      L[3] = m2l_fma(D[47], m, L[3]);
+    }
+    { const T m = __ldg(Ms + 28) * rp;
+      L[1] = m2l_fma(D[43], m, L[1]);
+      L[2] = m2l_fma(D[47], m, L[2]);
+      L[3] = m2l_fma(D[48], m, L[3]);
+    }
+    { const T m = __ldg(Ms + 29) * rp;
+      L[1] = m2l_fma(D[44], m, L[1]);
+      L[2] = m2l_fma(D[48], m, L[2]);
+      L[3] = m2l_fma(D[49], m, L[3]);
+    }
+    { const T m = __ldg(Ms + 30) * rp;
+      L[1] = m2l_fma(D[45], m, L[1]);
+      L[2] = m2l_fma(D[50], m, L[2]);
+      L[3] = m2l_fma(D[51], m, L[3]);
+    }
+    { const T m = __ldg(Ms + 31) * rp;
+      L[1] = m2l_fma(D[46], m, L[1]);
+      L[2] = m2l_fma(D[51], m, L[2]);
+      L[3] = m2l_fma(D[52], m, L[3]);
+    }
+    { const T m = __ldg(Ms + 32) * rp;
+      L[1] = m2l_fma(D[47], m, L[1]);
+      L[2] = m2l_fma(D[52], m, L[2]);
+      L[3] = m2l_fma(D[53], m, L[3]);
+    }
+    { const T m = __ldg(Ms + 33) * rp;
+      L[1] = m2l_fma(D[48], m, L[1]);
+      L[2] = m2l_fma(D[53], m, L[2]);
+      L[3] = m2l_fma(D[54], m, L[3]);
+    }
+    { const T m = __ldg(Ms + 34) * rp;
+      L[1] = m2l_fma(D[49], m, L[1]);
+      L[2] = m2l_fma(D[54], m, L[2]);
+      L[3] = m2l_fma(D[55], m, L[3]);
     }
 }
 
-__device__ __forceinline__ void m2l_side_b_forces_5(const float (&D)[56], const float *__restrict__ Ms, float (&L)[56])
+template <class T> __device__ __forceinline__ void m2l_side_b_forces_5(const T (&D)[56], const T *__restrict__ Ms, T (&L)[56])
 {
-    L[0] = 0.0f;
-    { const float m = __ldg(Ms + 0);
+    L[0] = T(0);
+    { const T m = __ldg(Ms + 0);
       L[1] = -D[1] * m;
       L[2] = -D[2] * m;
       L[3] = -D[3] * m;
@@ -3835,650 +3841,649 @@ __device__ __forceinline__ void m2l_side_b_forces_5(const float (&D)[56], const 
       L[54] = -D[54] * m;
       L[55] = -D[55] * m;
     }
-    { const float m = __ldg(Ms + 1);
-      L[1] = fmaf(-D[4], m, L[1]);
-      L[2] = fmaf(-D[5], m, L[2]);
-      L[3] = fmaf(-D[6], m, L[3]);
-      L[4] = fmaf(D[10], m, L[4]);
-      L[5] = fmaf(D[11], m, L[5]);
-      L[6] = fmaf(D[12], m, L[6]);
-      L[7] = fmaf(D[13], m, L[7]);
-      L[8] = fmaf(D[14], m, L[8]);
-      L[9] = fmaf(D[15], m, L[9]);
-      L[10] = fmaf(-D[20], m, L[10]);
-      L[11] = fmaf(-D[21], m, L[11]);
-      L[12] = fmaf(-D[22], m, L[12]);
-      L[13] = fmaf(-D[23], m, L[13]);
-      L[14] = fmaf(-D[24], m, L[14]);
-      L[15] = fmaf(-D[25], m, L[15]);
-      L[16] = fmaf(-D[26], m, L[16]);
-      L[17] = fmaf(-D[27], m, L[17]);
-      L[18] = fmaf(-D[28], m, L[18]);
-      L[19] = fmaf(-D[29], m, L[19]);
-      L[20] = fmaf(D[35], m, L[20]);
-      L[21] = fmaf(D[36], m, L[21]);
-      L[22] = fmaf(D[37], m, L[22]);
-      L[23] = fmaf(D[38], m, L[23]);
-      L[24] = fmaf(D[39], m, L[24]);
-      L[25] = fmaf(D[40], m, L[25]);
-      L[26] = fmaf(D[41], m, L[26]);
-      L[27] = fmaf(D[42], m, L[27]);
-      L[28] = fmaf(D[43], m, L[28]);
-      L[29] = fmaf(D[44], m, L[29]);
-      L[30] = fmaf(D[45], m, L[30]);
-      L[31] = fmaf(D[46], m, L[31]);
-      L[32] = fmaf(D[47], m, L[32]);
-      L[33] = fmaf(D[48], m, L[33]);
-      L[34] = fmaf(D[49], m, L[34]);
+    { const T m = __ldg(Ms + 1);
+      L[1] = m2l_fma(-D[4], m, L[1]);
+      L[2] = m2l_fma(-D[5], m, L[2]);
+      L[3] = m2l_fma(-D[6], m, L[3]);
+      L[4] = m2l_fma(D[10], m, L[4]);
+      L[5] = m2l_fma(D[11], m, L[5]);
+      L[6] = m2l_fma(D[12], m, L[6]);
+      L[7] = m2l_fma(D[13], m, L[7]);
+      L[8] = m2l_fma(D[14], m, L[8]);
+      L[9] = m2l_fma(D[15], m, L[9]);
+      L[10] = m2l_fma(-D[20], m, L[10]);
+      L[11] = m2l_fma(-D[21], m, L[11]);
+      L[12] = m2l_fma(-D[22], m, L[12]);
+      L[13] = m2l_fma(-D[23], m, L[13]);
+      L[14] = m2l_fma(-D[24], m, L[14]);
+      L[15] = m2l_fma(-D[25], m, L[15]);
+      L[16] = m2l_fma(-D[26], m, L[16]);
+      L[17] = m2l_fma(-D[27], m, L[17]);
+      L[18] = m2l_fma(-D[28], m, L[18]);
+      L[19] = m2l_fma(-D[29], m, L[19]);
+      L[20] = m2l_fma(D[35], m, L[20]);
+      L[21] = m2l_fma(D[36], m, L[21]);
+      L[22] = m2l_fma(D[37], m, L[22]);
+      L[23] = m2l_fma(D[38], m, L[23]);
+      L[24] = m2l_fma(D[39], m, L[24]);
+      L[25] = m2l_fma(D[40], m, L[25]);
+      L[26] = m2l_fma(D[41], m, L[26]);
+      L[27] = m2l_fma(D[42], m, L[27]);
+      L[28] = m2l_fma(D[43], m, L[28]);
+      L[29] = m2l_fma(D[44], m, L[29]);
+      L[30] = m2l_fma(D[45], m, L[30]);
+      L[31] = m2l_fma(D[46], m, L[31]);
+      L[32] = m2l_fma(D[47], m, L[32]);
+      L[33] = m2l_fma(D[48], m, L[33]);
+      L[34] = m2l_fma(D[49], m, L[34]);
     }
-    { const float m = __ldg(Ms + 2);
-      L[1] = fmaf(-D[5], m, L[1]);
-      L[2] = fmaf(-D[7], m, L[2]);
-      L[3] = fmaf(-D[8], m, L[3]);
-      L[4] = fmaf(D[11], m, L[4]);
-      L[5] = fmaf(D[13], m, L[5]);
-      L[6] = fmaf(D[14], m, L[6]);
-      L[7] = fmaf(D[16], m, L[7]);
-      L[8] = fmaf(D[17], m, L[8]);
-      L[9] = fmaf(D[18], m, L[9]);
-      L[10] = fmaf(-D[21], m, L[10]);
-      L[11] = fmaf(-D[23], m, L[11]);
-      L[12] = fmaf(-D[24], m, L[12]);
-      L[13] = fmaf(-D[26], m, L[13]);
-      L[14] = fmaf(-D[27], m, L[14]);
-      L[15] = fmaf(-D[28], m, L[15]);
-      L[16] = fmaf(-D[30], m, L[16]);
-      L[17] = fmaf(-D[31], m, L[17]);
-      L[18] = fmaf(-D[32], m, L[18]);
-      L[19] = fmaf(-D[33], m, L[19]);
-      L[20] = fmaf(D[36], m, L[20]);
-      L[21] = fmaf(D[38], m, L[21]);
-      L[22] = fmaf(D[39], m, L[22]);
-      L[23] = fmaf(D[41], m, L[23]);
-      L[24] = fmaf(D[42], m, L[24]);
-      L[25] = fmaf(D[43], m, L[25]);
-      L[26] = fmaf(D[45], m, L[26]);
-      L[27] = fmaf(D[46], m, L[27]);
-      L[28] = fmaf(D[47], m, L[28]);
-      L[29] = fmaf(D[48], m, L[29]);
-      L[30] = fmaf(D[50], m, L[30]);
-      L[31] = fmaf(D[51], m, L[31]);
-      L[32] = fmaf(D[52], m, L[32]);
-      L[33] = fmaf(D[53], m, L[33]);
-      L[34] = fmaf(D[54], m, L[34]);
+    { const T m = __ldg(Ms + 2);
+      L[1] = m2l_fma(-D[5], m, L[1]);
+      L[2] = m2l_fma(-D[7], m, L[2]);
+      L[3] = m2l_fma(-D[8], m, L[3]);
+      L[4] = m2l_fma(D[11], m, L[4]);
+      L[5] = m2l_fma(D[13], m, L[5]);
+      L[6] = m2l_fma(D[14], m, L[6]);
+      L[7] = m2l_fma(D[16], m, L[7]);
+      L[8] = m2l_fma(D[17], m, L[8]);
+      L[9] = m2l_fma(D[18], m, L[9]);
+      L[10] = m2l_fma(-D[21], m, L[10]);
+      L[11] = m2l_fma(-D[23], m, L[11]);
+      L[12] = m2l_fma(-D[24], m, L[12]);
+      L[13] = m2l_fma(-D[26], m, L[13]);
+      L[14] = m2l_fma(-D[27], m, L[14]);
+      L[15] = m2l_fma(-D[28], m, L[15]);
+      L[16] = m2l_fma(-D[30], m, L[16]);
+      L[17] = m2l_fma(-D[31], m, L[17]);
+      L[18] = m2l_fma(-D[32], m, L[18]);
+      L[19] = m2l_fma(-D[33], m, L[19]);
+      L[20] = m2l_fma(D[36], m, L[20]);
+      L[21] = m2l_fma(D[38], m, L[21]);
+      L[22] = m2l_fma(D[39], m, L[22]);
+      L[23] = m2l_fma(D[41], m, L[23]);
+      L[24] = m2l_fma(D[42], m, L[24]);
+      L[25] = m2l_fma(D[43], m, L[25]);
+      L[26] = m2l_fma(D[45], m, L[26]);
+      L[27] = m2l_fma(D[46], m, L[27]);
+      L[28] = m2l_fma(D[47], m, L[28]);
+      L[29] = m2l_fma(D[48], m, L[29]);
+      L[30] = m2l_fma(D[50], m, L[30]);
+      L[31] = m2l_fma(D[51], m, L[31]);
+      L[32] = m2l_fma(D[52], m, L[32]);
+      L[33] = m2l_fma(D[53], m, L[33]);
+      L[34] = m2l_fma(D[54], m, L[34]);
     }
-    { const float m = __ldg(Ms + 3);
-      L[1] = fmaf(-D[6], m, L[1]);
-      L[2] = fmaf(-D[8], m, L[2]);
-      L[3] = fmaf(-D[9], m, L[3]);
-      L[4] = fmaf(D[12], m, L[4]);
-      L[5] = fmaf(D[14], m, L[5]);
-      L[6] = fmaf(D[15], m, L[6]);
-      L[7] = fmaf(D[17], m, L[7]);
-      L[8] = fmaf(D[18], m, L[8]);
-      L[9] = fmaf(D[19], m, L[9]);
-      L[10] = fmaf(-D[22], m, L[10]);
-      L[11] = fmaf(-D[24], m, L[11]);
-      L[12] = fmaf(-D[25], m, L[12]);
-      L[13] = fmaf(-D[27], m, L[13]);
-      L[14] = fmaf(-D[28], m, L[14]);
-      L[15] = fmaf(-D[29], m, L[15]);
-      L[16] = fmaf(-D[31], m, L[16]);
-      L[17] = fmaf(-D[32], m, L[17]);
-      L[18] = fmaf(-D[33], m, L[18]);
-      L[19] = fmaf(-D[34], m, L[19]);
-      L[20] = fmaf(D[37], m, L[20]);
-      L[21] = fmaf(D[39], m, L[21]);
-      L[22] = fmaf(D[40], m, L[22]);
-      L[23] = fmaf(D[42], m, L[23]);
-      L[24] = fmaf(D[43], m, L[24]);
-      L[25] = fmaf(D[44], m, L[25]);
-      L[26] = fmaf(D[46], m, L[26]);
-      L[27] = fmaf(D[47], m, L[27]);
-      L[28] = fmaf(D[48], m, L[28]);
-      L[29] = fmaf(D[49], m, L[29]);
-      L[30] = fmaf(D[51], m, L[30]);
-      L[31] = fmaf(D[52], m, L[31]);
-      L[32] = fmaf(D[53], m, L[32]);
-      L[33] = fmaf(D[54], m, L[33]);
-      L[34] = fmaf(D[55], m, L[34]);
+    { const T m = __ldg(Ms + 3);
+      L[1] = m2l_fma(-D[6], m, L[1]);
+      L[2] = m2l_fma(-D[8], m, L[2]);
+      L[3] = m2l_fma(-D[9], m, L[3]);
+      L[4] = m2l_fma(D[12], m, L[4]);
+      L[5] = m2l_fma(D[14], m, L[5]);
+      L[6] = m2l_fma(D[15], m, L[6]);
+      L[7] = m2l_fma(D[17], m, L[7]);
+      L[8] = m2l_fma(D[18], m, L[8]);
+      L[9] = m2l_fma(D[19], m, L[9]);
+      L[10] = m2l_fma(-D[22], m, L[10]);
+      L[11] = m2l_fma(-D[24], m, L[11]);
+      L[12] = m2l_fma(-D[25], m, L[12]);
+      L[13] = m2l_fma(-D[27], m, L[13]);
+      L[14] = m2l_fma(-D[28], m, L[14]);
+      L[15] = m2l_fma(-D[29], m, L[15]);
+      L[16] = m2l_fma(-D[31], m, L[16]);
+      L[17] = m2l_fma(-D[32], m, L[17]);
+      L[18] = m2l_fma(-D[33], m, L[18]);
+      L[19] = m2l_fma(-D[34], m, L[19]);
+      L[20] = m2l_fma(D[37], m, L[20]);
+      L[21] = m2l_fma(D[39], m, L[21]);
+      L[22] = m2l_fma(D[40], m, L[22]);
+      L[23] = m2l_fma(D[42], m, L[23]);
+      L[24] = m2l_fma(D[43], m, L[24]);
+      L[25] = m2l_fma(D[44], m, L[25]);
+      L[26] = m2l_fma(D[46], m, L[26]);
+      L[27] = m2l_fma(D[47], m, L[27]);
+      L[28] = m2l_fma(D[48], m, L[28]);
+      L[29] = m2l_fma(D[49], m, L[29]);
+      L[30] = m2l_fma(D[51], m, L[30]);
+      L[31] = m2l_fma(D[52], m, L[31]);
+      L[32] = m2l_fma(D[53], m, L[32]);
+      L[33] = m2l_fma(D[54], m, L[33]);
+      L[34] = m2l_fma(D[55], m, L[34]);
     }
-    { const float m = __ldg(Ms + 4);
-      L[1] = fmaf(-D[10], m, L[1]);
-      L[2] = fmaf(-D[11], m, L[2]);
-      L[3] = fmaf(-D[12], m, L[3]);
-      L[4] = fmaf(D[20], m, L[4]);
-      L[5] = fmaf(D[21], m, L[5]);
-      L[6] = fmaf(D[22], m, L[6]);
-      L[7] = fmaf(D[23], m, L[7]);
-      L[8] = fmaf(D[24], m, L[8]);
-      L[9] = fmaf(D[25], m, L[9]);
-      L[10] = fmaf(-D[35], m, L[10]);
-      L[11] = fmaf(-D[36], m, L[11]);
-      L[12] = fmaf(-D[37], m, L[12]);
-      L[13] = fmaf(-D[38], m, L[13]);
-      L[14] = fmaf(-D[39], m, L[14]);
-      L[15] = fmaf(-D[40], m, L[15]);
-      L[16] = fmaf(-D[41], m, L[16]);
-      L[17] = fmaf(-D[42], m, L[17]);
-      L[18] = fmaf(-D[43], m, L[18]);
-      L[19] = fmaf(-D[44], m, L[19]);
+    { const T m = __ldg(Ms + 4);
+      L[1] = m2l_fma(-D[10], m, L[1]);
+      L[2] = m2l_fma(-D[11], m, L[2]);
+      L[3] = m2l_fma(-D[12], m, L[3]);
+      L[4] = m2l_fma(D[20], m, L[4]);
+      L[5] = m2l_fma(D[21], m, L[5]);
+      L[6] = m2l_fma(D[22], m, L[6]);
+      L[7] = m2l_fma(D[23], m, L[7]);
+      L[8] = m2l_fma(D[24], m, L[8]);
+      L[9] = m2l_fma(D[25], m, L[9]);
+      L[10] = m2l_fma(-D[35], m, L[10]);
+      L[11] = m2l_fma(-D[36], m, L[11]);
+      L[12] = m2l_fma(-D[37], m, L[12]);
+      L[13] = m2l_fma(-D[38], m, L[13]);
+      L[14] = m2l_fma(-D[39], m, L[14]);
+      L[15] = m2l_fma(-D[40], m, L[15]);
+      L[16] = m2l_fma(-D[41], m, L[16]);
+      L[17] = m2l_fma(-D[42], m, L[17]);
+      L[18] = m2l_fma(-D[43], m, L[18]);
+      L[19] = m2l_fma(-D[44], m, L[19]);
     }
-    { const float m = __ldg(Ms + 5);
-      L[1] = fmaf(-D[11], m, L[1]);
-      L[2] = fmaf(-D[13], m, L[2]);
-      L[3] = fmaf(-D[14], m, L[3]);
-      L[4] = fmaf(D[21], m, L[4]);
-      L[5] = fmaf(D[23], m, L[5]);
-      L[6] = fmaf(D[24], m, L[6]);
-      L[7] = fmaf(D[26], m, L[7]);
-      L[8] = fmaf(D[27], m, L[8]);
-      L[9] = fmaf(D[28], m, L[9]);
-      L[10] = fmaf(-D[36], m, L[10]);
-      L[11] = fmaf(-D[38], m, L[11]);
-      L[12] = fmaf(-D[39], m, L[12]);
-      L[13] = fmaf(-D[41], m, L[13]);
-      L[14] = fmaf(-D[42], m, L[14]);
-      L[15] = fmaf(-D[43], m, L[15]);
-      L[16] = fmaf(-D[45], m, L[16]);
-      L[17] = fmaf(-D[46], m, L[17]);
-      L[18] = fmaf(-D[47], m, L[18]);
-      L[19] = fmaf(-D[48], m, L[19]);
+    { const T m = __ldg(Ms + 5);
+      L[1] = m2l_fma(-D[11], m, L[1]);
+      L[2] = m2l_fma(-D[13], m, L[2]);
+      L[3] = m2l_fma(-D[14], m, L[3]);
+      L[4] = m2l_fma(D[21], m, L[4]);
+      L[5] = m2l_fma(D[23], m, L[5]);
+      L[6] = m2l_fma(D[24], m, L[6]);
+      L[7] = m2l_fma(D[26], m, L[7]);
+      L[8] = m2l_fma(D[27], m, L[8]);
+      L[9] = m2l_fma(D[28], m, L[9]);
+      L[10] = m2l_fma(-D[36], m, L[10]);
+      L[11] = m2l_fma(-D[38], m, L[11]);
+      L[12] = m2l_fma(-D[39], m, L[12]);
+      L[13] = m2l_fma(-D[41], m, L[13]);
+      L[14] = m2l_fma(-D[42], m, L[14]);
+      L[15] = m2l_fma(-D[43], m, L[15]);
+      L[16] = m2l_fma(-D[45], m, L[16]);
+      L[17] = m2l_fma(-D[46], m, L[17]);
+      L[18] = m2l_fma(-D[47], m, L[18]);
+      L[19] = m2l_fma(-D[48], m, L[19]);
     }
-    { const float m = __ldg(Ms + 6);
-      L[1] = fmaf(-D[12], m, L[1]);
-      L[2] = fmaf(-D[14], m, L[2]);
-      L[3] = fmaf(-D[15], m, L[3]);
-      L[4] = fmaf(D[22], m, L[4]);
-      L[5] = fmaf(D[24], m, L[5]);
-      L[6] = fmaf(D[25], m, L[6]);
-      L[7] = fmaf(D[27], m, L[7]);
-      L[8] = fmaf(D[28], m, L[8]);
-      L[9] = fmaf(D[29], m, L[9]);
-      L[10] = fmaf(-D[37], m, L[10]);
-      L[11] = fmaf(-D[39], m, L[11]);
-      L[12] = fmaf(-D[40], m, L[12]);
-      L[13] = fmaf(-D[42], m, L[13]);
-      L[14] = fmaf(-D[43], m, L[14]);
-      L[15] = fmaf(-D[44], m, L[15]);
-      L[16] = fmaf(-D[46], m, L[16]);
-      L[17] = fmaf(-D[47], m, L[17]);
-      L[18] = fmaf(-D[48], m, L[18]);
-      L[19] = fmaf(-D[49], m, L[19]);
+    { const T m = __ldg(Ms + 6);
+      L[1] = m2l_fma(-D[12], m, L[1]);
+      L[2] = m2l_fma(-D[14], m, L[2]);
+      L[3] = m2l_fma(-D[15], m, L[3]);
+      L[4] = m2l_fma(D[22], m, L[4]);
+      L[5] = m2l_fma(D[24], m, L[5]);
+      L[6] = m2l_fma(D[25], m, L[6]);
+      L[7] = m2l_fma(D[27], m, L[7]);
+      L[8] = m2l_fma(D[28], m, L[8]);
+      L[9] = m2l_fma(D[29], m, L[9]);
+      L[10] = m2l_fma(-D[37], m, L[10]);
+      L[11] = m2l_fma(-D[39], m, L[11]);
+      L[12] = m2l_fma(-D[40], m, L[12]);
+      L[13] = m2l_fma(-D[42], m, L[13]);
+      L[14] = m2l_fma(-D[43], m, L[14]);
+      L[15] = m2l_fma(-D[44], m, L[15]);
+      L[16] = m2l_fma(-D[46], m, L[16]);
+      L[17] = m2l_fma(-D[47], m, L[17]);
+      L[18] = m2l_fma(-D[48], m, L[18]);
+      L[19] = m2l_fma(-D[49], m, L[19]);
     }
-    { const float m = __ldg(Ms + 7);
-      L[1] = fmaf(-D[13], m, L[1]);
-      L[2] = fmaf(-D[16], m, L[2]);
-      L[3] = fmaf(-D[17], m, L[3]);
-      L[4] = fmaf(D[23], m, L[4]);
-      L[5] = fmaf(D[26], m, L[5]);
-      L[6] = fmaf(D[27], m, L[6]);
-      L[7] = fmaf(D[30], m, L[7]);
-      L[8] = fmaf(D[31], m, L[8]);
-      L[9] = fmaf(D[32], m, L[9]);
-      L[10] = fmaf(-D[38], m, L[10]);
-      L[11] = fmaf(-D[41], m, L[11]);
-      L[12] = fmaf(-D[42], m, L[12]);
-      L[13] = fmaf(-D[45], m, L[13]);
-      L[14] = fmaf(-D[46], m, L[14]);
-      L[15] = fmaf(-D[47], m, L[15]);
-      L[16] = fmaf(-D[50], m, L[16]);
-      L[17] = fmaf(-D[51], m, L[17]);
-      L[18] = fmaf(-D[52], m, L[18]);
-      L[19] = fmaf(-D[53], m, L[19]);
+    { const T m = __ldg(Ms + 7);
+      L[1] = m2l_fma(-D[13], m, L[1]);
+      L[2] = m2l_fma(-D[16], m, L[2]);
+      L[3] = m2l_fma(-D[17], m, L[3]);
+      L[4] = m2l_fma(D[23], m, L[4]);
+      L[5] = m2l_fma(D[26], m, L[5]);
+      L[6] = m2l_fma(D[27], m, L[6]);
+      L[7] = m2l_fma(D[30], m, L[7]);
+      L[8] = m2l_fma(D[31], m, L[8]);
+      L[9] = m2l_fma(D[32], m, L[9]);
+      L[10] = m2l_fma(-D[38], m, L[10]);
+      L[11] = m2l_fma(-D[41], m, L[11]);
+      L[12] = m2l_fma(-D[42], m, L[12]);
+      L[13] = m2l_fma(-D[45], m, L[13]);
+      L[14] = m2l_fma(-D[46], m, L[14]);
+      L[15] = m2l_fma(-D[47], m, L[15]);
+      L[16] = m2l_fma(-D[50], m, L[16]);
+      L[17] = m2l_fma(-D[51], m, L[17]);
+      L[18] = m2l_fma(-D[52], m, L[18]);
+      L[19] = m2l_fma(-D[53], m, L[19]);
     }
-    { const float m = __ldg(Ms + 8);
-      L[1] = fmaf(-D[14], m, L[1]);
-      L[2] = fmaf(-D[17], m, L[2]);
-      L[3] = fmaf(-D[18], m, L[3]);
-      L[4] = fmaf(D[24], m, L[4]);
-      L[5] = fmaf(D[27], m, L[5]);
-      L[6] = fmaf(D[28], m, L[6]);
-      L[7] = fmaf(D[31], m, L[7]);
-      L[8] = fmaf(D[32], m, L[8]);
-      L[9] = fmaf(D[33], m, L[9]);
-      L[10] = fmaf(-D[39], m, L[10]);
-      L[11] = fmaf(-D[42], m, L[11]);
-      L[12] = fmaf(-D[43], m, L[12]);
-      L[13] = fmaf(-D[46], m, L[13]);
-      L[14] = fmaf(-D[47], m, L[14]);
-      L[15] = fmaf(-D[48], m, L[15]);
-      L[16] = fmaf(-D[51], m, L[16]);
-      L[17] = fmaf(-D[52], m, L[17]);
-      L[18] = fmaf(-D[53], m, L[18]);
-      L[19] = fmaf(-D[54], m, L[19]);
+    { const T m = __ldg(Ms + 8);
+      L[1] = m2l_fma(-D[14], m, L[1]);
+      L[2] = m2l_fma(-D[17], m, L[2]);
+      L[3] = m2l_fma(-D[18], m, L[3]);
+      L[4] = m2l_fma(D[24], m, L[4]);
+      L[5] = m2l_fma(D[27], m, L[5]);
+      L[6] = m2l_fma(D[28], m, L[6]);
+      L[7] = m2l_fma(D[31], m, L[7]);
+      L[8] = m2l_fma(D[32], m, L[8]);
+      L[9] = m2l_fma(D[33], m, L[9]);
+      L[10] = m2l_fma(-D[39], m, L[10]);
+      L[11] = m2l_fma(-D[42], m, L[11]);
+      L[12] = m2l_fma(-D[43], m, L[12]);
+      L[13] = m2l_fma(-D[46], m, L[13]);
+      L[14] = m2l_fma(-D[47], m, L[14]);
+      L[15] = m2l_fma(-D[48], m, L[15]);
+      L[16] = m2l_fma(-D[51], m, L[16]);
+      L[17] = m2l_fma(-D[52], m, L[17]);
+      L[18] = m2l_fma(-D[53], m, L[18]);
+      L[19] = m2l_fma(-D[54], m, L[19]);
     }
-    { const float m = __ldg(Ms + 9);
-      L[1] = fmaf(-D[15], m, L[1]);
-      L[2] = fmaf(-D[18], m, L[2]);
-      L[3] = fmaf(-D[19], m, L[3]);
-      L[4] = fmaf(D[25], m, L[4]);
-      L[5] = fmaf(D[28], m, L[5]);
-      L[6] = fmaf(D[29], m, L[6]);
-      L[7] = fmaf(D[32], m, L[7]);
-      L[8] = fmaf(D[33], m, L[8]);
-      L[9] = fmaf(D[34], m, L[9]);
-      L[10] = fmaf(-D[40], m, L[10]);
-      L[11] = fmaf(-D[43], m, L[11]);
-      L[12] = fmaf(-D[44], m, L[12]);
-      L[13] = fmaf(-D[47], m, L[13]);
-      L[14] = fmaf(-D[48], m, L[14]);
-      L[15] = fmaf(-D[49], m, L[15]);
-      L[16] = fmaf(-D[52], m, L[16]);
-      L[17] = fmaf(-D[53], m, L[17]);
-      L[18] = fmaf(-D[54], m, L[18]);
-      L[19] = fmaf(-D[55], m, L[19]);
+    { const T m = __ldg(Ms + 9);
+      L[1] = m2l_fma(-D[15], m, L[1]);
+      L[2] = m2l_fma(-D[18], m, L[2]);
+      L[3] = m2l_fma(-D[19], m, L[3]);
+      L[4] = m2l_fma(D[25], m, L[4]);
+      L[5] = m2l_fma(D[28], m, L[5]);
+      L[6] = m2l_fma(D[29], m, L[6]);
+      L[7] = m2l_fma(D[32], m, L[7]);
+      L[8] = m2l_fma(D[33], m, L[8]);
+      L[9] = m2l_fma(D[34], m, L[9]);
+      L[10] = m2l_fma(-D[40], m, L[10]);
+      L[11] = m2l_fma(-D[43], m, L[11]);
+      L[12] = m2l_fma(-D[44], m, L[12]);
+      L[13] = m2l_fma(-D[47], m, L[13]);
+      L[14] = m2l_fma(-D[48], m, L[14]);
+      L[15] = m2l_fma(-D[49], m, L[15]);
+      L[16] = m2l_fma(-D[52], m, L[16]);
+      L[17] = m2l_fma(-D[53], m, L[17]);
+      L[18] = m2l_fma(-D[54], m, L[18]);
+      L[19] = m2l_fma(-D[55], m, L[19]);
     }
-    { const float m = __ldg(Ms + 10);
-      L[1] = fmaf(-D[20], m, L[1]);
-      L[2] = fmaf(-D[21], m, L[2]);
-      L[3] = fmaf(-D[22], m, L[3]);
-      L[4] = fmaf(D[35], m, L[4]);
-      L[5] = fmaf(D[36], m, L[5]);
-      L[6] = fmaf(D[37], m, L[6]);
-      L[7] = fmaf(D[38], m, L[7]);
-      L[8] = fmaf(D[39], m, L[8]);
-      L[9] = fmaf(D[40], m, L[9]);
+    { const T m = __ldg(Ms + 10);
+      L[1] = m2l_fma(-D[20], m, L[1]);
+      L[2] = m2l_fma(-D[21], m, L[2]);
+      L[3] = m2l_fma(-D[22], m, L[3]);
+      L[4] = m2l_fma(D[35], m, L[4]);
+      L[5] = m2l_fma(D[36], m, L[5]);
+      L[6] = m2l_fma(D[37], m, L[6]);
+      L[7] = m2l_fma(D[38], m, L[7]);
+      L[8] = m2l_fma(D[39], m, L[8]);
+      L[9] = m2l_fma(D[40], m, L[9]);
     }
-    { const float m = __ldg(Ms + 11);
-      L[1] = fmaf(-D[21], m, L[1]);
-      L[2] = fmaf(-D[23], m, L[2]);
-      L[3] = fmaf(-D[24], m, L[3]);
-      L[4] = fmaf(D[36], m, L[4]);
-      L[5] = fmaf(D[38], m, L[5]);
-      L[6] = fmaf(D[39], m, L[6]);
-      L[7] = fmaf(D[41], m, L[7]);
-      L[8] = fmaf(D[42], m, L[8]);
-      L[9] = fmaf(D[43], m, L[9]);
+    { const T m = __ldg(Ms + 11);
+      L[1] = m2l_fma(-D[21], m, L[1]);
+      L[2] = m2l_fma(-D[23], m, L[2]);
+      L[3] = m2l_fma(-D[24], m, L[3]);
+      L[4] = m2l_fma(D[36], m, L[4]);
+      L[5] = m2l_fma(D[38], m, L[5]);
+      L[6] = m2l_fma(D[39], m, L[6]);
+      L[7] = m2l_fma(D[41], m, L[7]);
+      L[8] = m2l_fma(D[42], m, L[8]);
+      L[9] = m2l_fma(D[43], m, L[9]);
     }
-    { const float m = __ldg(Ms + 12);
-      L[1] = fmaf(-D[22], m, L[1]);
-      L[2] = fmaf(-D[24], m, L[2]);
-      L[3] = fmaf(-D[25], m, L[3]);
-      L[4] = fmaf(D[37], m, L[4]);
-      L[5] = fmaf(D[39], m, L[5]);
-      L[6] = fmaf(D[40], m, L[6]);
-      L[7] = fmaf(D[42], m, L[7]);
-      L[8] = fmaf(D[43], m, L[8]);
-      L[9] = fmaf(D[44], m, L[9]);
+    { const T m = __ldg(Ms + 12);
+      L[1] = m2l_fma(-D[22], m, L[1]);
+      L[2] = m2l_fma(-D[24], m, L[2]);
+      L[3] = m2l_fma(-D[25], m, L[3]);
+      L[4] = m2l_fma(D[37], m, L[4]);
+      L[5] = m2l_fma(D[39], m, L[5]);
+      L[6] = m2l_fma(D[40], m, L[6]);
+      L[7] = m2l_fma(D[42], m, L[7]);
+      L[8] = m2l_fma(D[43], m, L[8]);
+      L[9] = m2l_fma(D[44], m, L[9]);
     }
-    { const float m = __ldg(Ms + 13);
-      L[1] = fmaf(-D[23], m, L[1]);
-      L[2] = fmaf(-D[26], m, L[2]);
-      L[3] = fmaf(-D[27], m, L[3]);
-      L[4] = fmaf(D[38], m, L[4]);
-      L[5] = fmaf(D[41], m, L[5]);
-      L[6] = fmaf(D[42], m, L[6]);
-      L[7] = fmaf(D[45], m, L[7]);
-      L[8] = fmaf(D[46], m, L[8]);
-      L[9] = fmaf(D[47], m, L[9]);
+    { const T m = __ldg(Ms + 13);
+      L[1] = m2l_fma(-D[23], m, L[1]);
+      L[2] = m2l_fma(-D[26], m, L[2]);
+      L[3] = m2l_fma(-D[27], m, L[3]);
+      L[4] = m2l_fma(D[38], m, L[4]);
+      L[5] = m2l_fma(D[41], m, L[5]);
+      L[6] = m2l_fma(D[42], m, L[6]);
+      L[7] = m2l_fma(D[45], m, L[7]);
+      L[8] = m2l_fma(D[46], m, L[8]);
+      L[9] = m2l_fma(D[47], m, L[9]);
     }
-    { const float m = __ldg(Ms + 14);
-      L[1] = fmaf(-D[24], m, L[1]);
-      L[2] = fmaf(-D[27], m, L[2]);
-      L[3] = fmaf(-D[28], m, L[3]);
-      L[4] = fmaf(D[39], m, L[4]);
-      L[5] = fmaf(D[42], m, L[5]);
-      L[6] = fmaf(D[43], m, L[6]);
-      L[7] = fmaf(D[46], m, L[7]);
-      L[8] = fmaf(D[47], m, L[8]);
-      L[9] = fmaf(D[48], m, L[9]);
+    { const T m = __ldg(Ms + 14);
+      L[1] = m2l_fma(-D[24], m, L[1]);
+      L[2] = m2l_fma(-D[27], m, L[2]);
+      L[3] = m2l_fma(-D[28], m, L[3]);
+      L[4] = m2l_fma(D[39], m, L[4]);
+      L[5] = m2l_fma(D[42], m, L[5]);
+      L[6] = m2l_fma(D[43], m, L[6]);
+      L[7] = m2l_fma(D[46], m, L[7]);
+      L[8] = m2l_fma(D[47], m, L[8]);
+      L[9] = m2l_fma(D[48], m, L[9]);
     }
-    { const float m = __ldg(Ms + 15);
-      L[1] = fmaf(-D[25], m, L[1]);
-      L[2] = fmaf(-D[28], m, L[2]);
-      L[3] = fmaf(-D[29], m, L[3]);
-      L[4] = fmaf(D[40], m, L[4]);
-      L[5] = fmaf(D[43], m, L[5]);
-      L[6] = fmaf(D[44], m, L[6]);
-      L[7] = fmaf(D[47], m, L[7]);
-      L[8] = fmaf(D[48], m, L[8]);
-      L[9] = fmaf(D[49], m, L[9]);
+    { const T m = __ldg(Ms + 15);
+      L[1] = m2l_fma(-D[25], m, L[1]);
+      L[2] = m2l_fma(-D[28], m, L[2]);
+      L[3] = m2l_fma(-D[29], m, L[3]);
+      L[4] = m2l_fma(D[40], m, L[4]);
+      L[5] = m2l_fma(D[43], m, L[5]);
+      L[6] = m2l_fma(D[44], m, L[6]);
+      L[7] = m2l_fma(D[47], m, L[7]);
+      L[8] = m2l_fma(D[48], m, L[8]);
+      L[9] = m2l_fma(D[49], m, L[9]);
     }
-    { const float m = __ldg(Ms + 16);
-      L[1] = fmaf(-D[26], m, L[1]);
-      L[2] = fmaf(-D[30], m, L[2]);
-      L[3] = fmaf(-D[31], m, L[3]);
-      L[4] = fmaf(D[41], m, L[4]);
-      L[5] = fmaf(D[45], m, L[5]);
-      L[6] = fmaf(D[46], m, L[6]);
-      L[7] = fmaf(D[50], m, L[7]);
-      L[8] = fmaf(D[51], m, L[8]);
-      L[9] = fmaf(D[52], m, L[9]);
+    { const T m = __ldg(Ms + 16);
+      L[1] = m2l_fma(-D[26], m, L[1]);
+      L[2] = m2l_fma(-D[30], m, L[2]);
+      L[3] = m2l_fma(-D[31], m, L[3]);
+      L[4] = m2l_fma(D[41], m, L[4]);
+      L[5] = m2l_fma(D[45], m, L[5]);
+      L[6] = m2l_fma(D[46], m, L[6]);
+      L[7] = m2l_fma(D[50], m, L[7]);
+      L[8] = m2l_fma(D[51], m, L[8]);
+      L[9] = m2l_fma(D[52], m, L[9]);
     }
-    { const float m = __ldg(Ms + 17);
-      L[1] = fmaf(-D[27], m, L[1]);
-      L[2] = fmaf(-D[31], m, L[2]);
-      L[3] = fmaf(-D[32], m, L[3]);
-      L[4] = fmaf(D[42], m, L[4]);
-      L[5] = fmaf(D[46], m, L[5]);
-      L[6] = fmaf(D[47], m, L[6]);
-      L[7] = fmaf(D[51], m, L[7]);
-      L[8] = fmaf(D[52], m, L[8]);
-      L[9] = fmaf(D[53], m, L[9]);
+    { const T m = __ldg(Ms + 17);
+      L[1] = m2l_fma(-D[27], m, L[1]);
+      L[2] = m2l_fma(-D[31], m, L[2]);
+      L[3] = m2l_fma(-D[32], m, L[3]);
+      L[4] = m2l_fma(D[42], m, L[4]);
+      L[5] = m2l_fma(D[46], m, L[5]);
+      L[6] = m2l_fma(D[47], m, L[6]);
+      L[7] = m2l_fma(D[51], m, L[7]);
+      L[8] = m2l_fma(D[52], m, L[8]);
+      L[9] = m2l_fma(D[53], m, L[9]);
     }
-    { const float m = __ldg(Ms + 18);
-      L[1] = fmaf(-D[28], m, L[1]);
-      L[2] = fmaf(-D[32], m, L[2]);
-      L[3] = fmaf(-D[33], m, L[3]);
-      L[4] = fmaf(D[43], m, L[4]);
-      L[5] = fmaf(D[47], m, L[5]);
-      L[6] = fmaf(D[48], m, L[6]);
-      L[7] = fmaf(D[52], m, L[7]);
-      L[8] = fmaf(D[53], m, L[8]);
-      L[9] = fmaf(D[54], m, L[9]);
+    { const T m = __ldg(Ms + 18);
+      L[1] = m2l_fma(-D[28], m, L[1]);
+      L[2] = m2l_fma(-D[32], m, L[2]);
+      L[3] = m2l_fma(-D[33], m, L[3]);
+      L[4] = m2l_fma(D[43], m, L[4]);
+      L[5] = m2l_fma(D[47], m, L[5]);
+      L[6] = m2l_fma(D[48], m, L[6]);
+      L[7] = m2l_fma(D[52], m, L[7]);
+      L[8] = m2l_fma(D[53], m, L[8]);
+      L[9] = m2l_fma(D[54], m, L[9]);
     }
-    { const float m = __ldg(Ms + 19);
-      L[1] = fmaf(-D[29], m, L[1]);
-      L[2] = fmaf(-D[33], m, L[2]);
-      L[3] = fmaf(-D[34], m, L[3]);
-      L[4] = fmaf(D[44], m, L[4]);
-      L[5] = fmaf(D[48], m, L[5]);
-      L[6] = fmaf(D[49], m, L[6]);
-      L[7] = fmaf(D[53], m, L[7]);
-      L[8] = fmaf(D[54], m, L[8]);
-      L[9] = fmaf(D[55], m, L[9]);
+    { const T m = __ldg(Ms + 19);
+      L[1] = m2l_fma(-D[29], m, L[1]);
+      L[2] = m2l_fma(-D[33], m, L[2]);
+      L[3] = m2l_fma(-D[34], m, L[3]);
+      L[4] = m2l_fma(D[44], m, L[4]);
+      L[5] = m2l_fma(D[48], m, L[5]);
+      L[6] = m2l_fma(D[49], m, L[6]);
+      L[7] = m2l_fma(D[53], m, L[7]);
+      L[8] = m2l_fma(D[54], m, L[8]);
+      L[9] = m2l_fma(D[55], m, L[9]);
     }
-    { const float m = __ldg(Ms + 20);
-      L[1] = fmaf(-D[35], m, L[1]);
-      L[2] = fmaf(-D[36], m, L[2]);
-      L[3] = fmaf(-D[37], m, L[3]);
+    { const T m = __ldg(Ms + 20);
+      L[1] = m2l_fma(-D[35], m, L[1]);
+      L[2] = m2l_fma(-D[36], m, L[2]);
+      L[3] = m2l_fma(-D[37], m, L[3]);
     }
-    { const float m = __ldg(Ms + 21);
-      L[1] = fmaf(-D[36], m, L[1]);
-      L[2] = fmaf(-D[38], m, L[2]);
-      L[3] = fmaf(-D[39], m, L[3]);
+    { const T m = __ldg(Ms + 21);
+      L[1] = m2l_fma(-D[36], m, L[1]);
+      L[2] = m2l_fma(-D[38], m, L[2]);
+      L[3] = m2l_fma(-D[39], m, L[3]);
     }
-    { const float m = __ldg(Ms + 22);
-      L[1] = fmaf(-D[37], m, L[1]);
-      L[2] = fmaf(-D[39], m, L[2]);
-      L[3] = fmaf(-D[40], m, L[3]);
+    { const T m = __ldg(Ms + 22);
+      L[1] = m2l_fma(-D[37], m, L[1]);
+      L[2] = m2l_fma(-D[39], m, L[2]);
+      L[3] = m2l_fma(-D[40], m, L[3]);
     }
-    { const float m = __ldg(Ms + 23);
-      L[1] = fmaf(-D[38], m, L[1]);
-      L[2] = fmaf(-D[41], m, L[2]);
-      L[3] = fmaf(-D[42], m, L[3]);
+    { const T m = __ldg(Ms + 23);
+      L[1] = m2l_fma(-D[38], m, L[1]);
+      L[2] = m2l_fma(-D[41], m, L[2]);
+      L[3] = m2l_fma(-D[42], m, L[3]);
     }
-    { const float m = __ldg(Ms + 24);
-      L[1] = fmaf(-D[39], m, L[1]);
-      L[2] = fmaf(-D[42], m, L[2]);
-      L[3] = fmaf(-D[43], m, L[3]);
+    { const T m = __ldg(Ms + 24);
+      L[1] = m2l_fma(-D[39], m, L[1]);
+      L[2] = m2l_fma(-D[42], m, L[2]);
+      L[3] = m2l_fma(-D[43], m, L[3]);
     }
-    { const float m = __ldg(Ms + 25);
-      L[1] = fmaf(-D[40], m, L[1]);
-      L[2] = fmaf(-D[43], m, L[2]);
-      L[3] = fmaf(-D[44], m, L[3]);
+    { const T m = __ldg(Ms + 25);
+      L[1] = m2l_fma(-D[40], m, L[1]);
+      L[2] = m2l_fma(-D[43], m, L[2]);
+      L[3] = m2l_fma(-D[44], m, L[3]);
     }
-    { const float m = __ldg(Ms + 26);
-      L[1] = fmaf(-D[41], m, L[1]);
-      L[2] = fmaf(-D[45], m, L[2]);
-      L[3] = fmaf(-D[46], m, L[3]);
+    { const T m = __ldg(Ms + 26);
+      L[1] = m2l_fma(-D[41], m, L[1]);
+      L[2] = m2l_fma(-D[45], m, L[2]);
+      L[3] = m2l_fma(-D[46], m, L[3]);
     }
-    { const float m = __ldg(Ms + 27);
-      L[1] = fmaf(-D[42], m, L[1]);
-      L[2] = fmaf(-D[46], m, L[2]);
-      L[3] = fmaf(-D[47], m, L[3]);
+    { const T m = __ldg(Ms + 27);
+      L[1] = m2l_fma(-D[42], m, L[1]);
+      L[2] = m2l_fma(-D[46], m, L[2]);
+      L[3] = m2l_fma(-D[47], m, L[3]);
     }
-    { const float m = __ldg(Ms + 28);
-      L[1] = fmaf(-D[43], m, L[1]);
-      L[2] = fmaf(-D[47], m, L[2]);
-      L[3] = fmaf(-D[48], m, L[3]);
+    { const T m = __ldg(Ms + 28);
+      L[1] = m2l_fma(-D[43], m, L[1]);
+      L[2] = m2l_fma(-D[47], m, L[2]);
+      L[3] = m2l_fma(-D[48], m, L[3]);
     }
-    { const float m = __ldg(Ms + 29);
-      L[1] = fmaf(-D[44], m, L[1]);
-      L[2] = fmaf(-D[48], m, L[2]);
-      L[3] = fmaf(-D[49], m, L[3]);
+    { const T m = __ldg(Ms + 29);
+      L[1] = m2l_fma(-D[44], m, L[1]);
+      L[2] = m2l_fma(-D[48], m, L[2]);
+      L[3] = m2l_fma(-D[49], m, L[3]);
     }
-    { const float m = __ldg(Ms + 30);
-      L[1] = fmaf(-D[45], m, L[1]);
-      L[2] = fmaf(-D[50], m, L[2]);
-      L[3] = fmaf(-D[51], m, L[3]);
+    { const T m = __ldg(Ms + 30);
+      L[1] = m2l_fma(-D[45], m, L[1]);
+      L[2] = m2l_fma(-D[50], m, L[2]);
+      L[3] = m2l_fma(-D[51], m, L[3]);
     }
-    { const float m = __ldg(Ms + 31);
-      L[1] = fmaf(-D[46], m, L[1]);
-      L[2] = fmaf(-D[51], m, L[2]);
-      L[3] = fmaf(-D[52], m, L[3]);
+    { const T m = __ldg(Ms + 31);
+      L[1] = m2l_fma(-D[46], m, L[1]);
+      L[2] = m2l_fma(-D[51], m, L[2]);
+      L[3] = m2l_fma(-D[52], m, L[3]);
     }
-    { const float m = __ldg(Ms + 32);
-      L[1] = fmaf(-D[47], m, L[1]);
-      L[2] = fmaf(-D[52], m, L[2]);
-      L[3] = fmaf(-D[53], m, L[3]);
+    { const T m = __ldg(Ms + 32);
+      L[1] = m2l_fma(-D[47], m, L[1]);
+      L[2] = m2l_fma(-D[52], m, L[2]);
+      L[3] = m2l_fma(-D[53], m, L[3]);
     }
-    { const float m = __ldg(Ms + 33);
-      L[1] = fmaf(-D[48], m, L[1]);
-      L[2] = fmaf(-D[53], m, L[2]);
-      L[3] = fmaf(-D[54], m, L[3]);
+    { const T m = __ldg(Ms + 33);
+      L[1] = m2l_fma(-D[48], m, L[1]);
+      L[2] = m2l_fma(-D[53], m, L[2]);
+      L[3] = m2l_fma(-D[54], m, L[3]);
     }
-    { const float m = __ldg(Ms + 34);
-      L[1] = fmaf(-D[49], m, L[1]);
-      L[2] = fmaf(-D[54], m, L[2]);
-      L[3] = fmaf(-D[55], m, L[3]);
+    { const T m = __ldg(Ms + 34);
+      L[1] = m2l_fma(-D[49], m, L[1]);
+      L[2] = m2l_fma(-D[54], m, L[2]);
+      L[3] = m2l_fma(-D[55], m, L[3]);
     }
 }
 
-__device__ __forceinline__ void m2l_dtensor_6(float dx, float dy, float dz, float soft2, float (&D)[84])
+template <class T> __device__ __forceinline__ void m2l_dtensor_6(T dx, T dy, T dz, T soft2, T (&D)[84])
 {
-    const float s2 = fmaf(dx, dx, fmaf(dy, dy, fmaf(dz, dz, soft2)));
-    float si = rsqrtf(s2);
-    si = si * fmaf(-0.5f * s2, si * si, 1.5f);   // one Newton step
-    const float si2 = si * si;
-    const float f0 = -si;
-    const float f1 = -1.0f * f0 * si2;
-    const float f2 = -3.0f * f1 * si2;
-    const float f3 = -5.0f * f2 * si2;
-    const float f4 = -7.0f * f3 * si2;
-    const float f5 = -9.0f * f4 * si2;
-    const float f6 = -11.0f * f5 * si2;
-    const float r_0_0 = f0;
-    const float r_1_0 = f1;
-    const float r_2_0 = f2;
-    const float r_3_0 = f3;
-    const float r_4_0 = f4;
-    const float r_5_0 = f5;
-    const float r_6_0 = f6;
-    const float r_0_1 = dx * r_1_0;
-    const float r_1_1 = dx * r_2_0;
-    const float r_2_1 = dx * r_3_0;
-    const float r_3_1 = dx * r_4_0;
-    const float r_4_1 = dx * r_5_0;
-    const float r_5_1 = dx * r_6_0;
-    const float r_0_2 = dy * r_1_0;
-    const float r_1_2 = dy * r_2_0;
-    const float r_2_2 = dy * r_3_0;
-    const float r_3_2 = dy * r_4_0;
-    const float r_4_2 = dy * r_5_0;
-    const float r_5_2 = dy * r_6_0;
-    const float r_0_3 = dz * r_1_0;
-    const float r_1_3 = dz * r_2_0;
-    const float r_2_3 = dz * r_3_0;
-    const float r_3_3 = dz * r_4_0;
-    const float r_4_3 = dz * r_5_0;
-    const float r_5_3 = dz * r_6_0;
-    const float r_0_4 = fmaf(1.0f, r_1_0, dx * r_1_1);
-    const float r_1_4 = fmaf(1.0f, r_2_0, dx * r_2_1);
-    const float r_2_4 = fmaf(1.0f, r_3_0, dx * r_3_1);
-    const float r_3_4 = fmaf(1.0f, r_4_0, dx * r_4_1);
-    const float r_4_4 = fmaf(1.0f, r_5_0, dx * r_5_1);
-    const float r_0_5 = dx * r_1_2;
-    const float r_1_5 = dx * r_2_2;
-    const float r_2_5 = dx * r_3_2;
-    const float r_3_5 = dx * r_4_2;
-    const float r_4_5 = dx * r_5_2;
-    const float r_0_6 = dx * r_1_3;
-    const float r_1_6 = dx * r_2_3;
-    const float r_2_6 = dx * r_3_3;
-    const float r_3_6 = dx * r_4_3;
-    const float r_4_6 = dx * r_5_3;
-    const float r_0_7 = fmaf(1.0f, r_1_0, dy * r_1_2);
-    const float r_1_7 = fmaf(1.0f, r_2_0, dy * r_2_2);
-    const float r_2_7 = fmaf(1.0f, r_3_0, dy * r_3_2);
-    const float r_3_7 = fmaf(1.0f, r_4_0, dy * r_4_2);
-    const float r_4_7 = fmaf(1.0f, r_5_0, dy * r_5_2);
-    const float r_0_8 = dy * r_1_3;
-    const float r_1_8 = dy * r_2_3;
-    const float r_2_8 = dy * r_3_3;
-    const float r_3_8 = dy * r_4_3;
-    const float r_4_8 = dy * r_5_3;
-    const float r_0_9 = fmaf(1.0f, r_1_0, dz * r_1_3);
-    const float r_1_9 = fmaf(1.0f, r_2_0, dz * r_2_3);
-    const float r_2_9 = fmaf(1.0f, r_3_0, dz * r_3_3);
-    const float r_3_9 = fmaf(1.0f, r_4_0, dz * r_4_3);
-    const float r_4_9 = fmaf(1.0f, r_5_0, dz * r_5_3);
-    const float r_0_10 = fmaf(2.0f, r_1_1, dx * r_1_4);
-    const float r_1_10 = fmaf(2.0f, r_2_1, dx * r_2_4);
-    const float r_2_10 = fmaf(2.0f, r_3_1, dx * r_3_4);
-    const float r_3_10 = fmaf(2.0f, r_4_1, dx * r_4_4);
-    const float r_0_11 = fmaf(1.0f, r_1_2, dx * r_1_5);
-    const float r_1_11 = fmaf(1.0f, r_2_2, dx * r_2_5);
-    const float r_2_11 = fmaf(1.0f, r_3_2, dx * r_3_5);
-    const float r_3_11 = fmaf(1.0f, r_4_2, dx * r_4_5);
-    const float r_0_12 = fmaf(1.0f, r_1_3, dx * r_1_6);
-    const float r_1_12 = fmaf(1.0f, r_2_3, dx * r_2_6);
-    const float r_2_12 = fmaf(1.0f, r_3_3, dx * r_3_6);
-    const float r_3_12 = fmaf(1.0f, r_4_3, dx * r_4_6);
-    const float r_0_13 = dx * r_1_7;
-    const float r_1_13 = dx * r_2_7;
-    const float r_2_13 = dx * r_3_7;
-    const float r_3_13 = dx * r_4_7;
-    const float r_0_14 = dx * r_1_8;
-    const float r_1_14 = dx * r_2_8;
-    const float r_2_14 = dx * r_3_8;
-    const float r_3_14 = dx * r_4_8;
-    const float r_0_15 = dx * r_1_9;
-    const float r_1_15 = dx * r_2_9;
-    const float r_2_15 = dx * r_3_9;
-    const float r_3_15 = dx * r_4_9;
-    const float r_0_16 = fmaf(2.0f, r_1_2, dy * r_1_7);
-    const float r_1_16 = fmaf(2.0f, r_2_2, dy * r_2_7);
-    const float r_2_16 = fmaf(2.0f, r_3_2, dy * r_3_7);
-    const float r_3_16 = fmaf(2.0f, r_4_2, dy * r_4_7);
-    const float r_0_17 = fmaf(1.0f, r_1_3, dy * r_1_8);
-    const float r_1_17 = fmaf(1.0f, r_2_3, dy * r_2_8);
-    const float r_2_17 = fmaf(1.0f, r_3_3, dy * r_3_8);
-    const float r_3_17 = fmaf(1.0f, r_4_3, dy * r_4_8);
-    const float r_0_18 = dy * r_1_9;
-    const float r_1_18 = dy * r_2_9;
-    const float r_2_18 = dy * r_3_9;
-    const float r_3_18 = dy * r_4_9;
-    const float r_0_19 = fmaf(2.0f, r_1_3, dz * r_1_9);
-    const float r_1_19 = fmaf(2.0f, r_2_3, dz * r_2_9);
-    const float r_2_19 = fmaf(2.0f, r_3_3, dz * r_3_9);
-    const float r_3_19 = fmaf(2.0f, r_4_3, dz * r_4_9);
-    const float r_0_20 = fmaf(3.0f, r_1_4, dx * r_1_10);
-    const float r_1_20 = fmaf(3.0f, r_2_4, dx * r_2_10);
-    const float r_2_20 = fmaf(3.0f, r_3_4, dx * r_3_10);
-    const float r_0_21 = fmaf(2.0f, r_1_5, dx * r_1_11);
-    const float r_1_21 = fmaf(2.0f, r_2_5, dx * r_2_11);
-    const float r_2_21 = fmaf(2.0f, r_3_5, dx * r_3_11);
-    const float r_0_22 = fmaf(2.0f, r_1_6, dx * r_1_12);
-    const float r_1_22 = fmaf(2.0f, r_2_6, dx * r_2_12);
-    const float r_2_22 = fmaf(2.0f, r_3_6, dx * r_3_12);
-    const float r_0_23 = fmaf(1.0f, r_1_7, dx * r_1_13);
-    const float r_1_23 = fmaf(1.0f, r_2_7, dx * r_2_13);
-    const float r_2_23 = fmaf(1.0f, r_3_7, dx * r_3_13);
-    const float r_0_24 = fmaf(1.0f, r_1_8, dx * r_1_14);
-    const float r_1_24 = fmaf(1.0f, r_2_8, dx * r_2_14);
-    const float r_2_24 = fmaf(1.0f, r_3_8, dx * r_3_14);
-    const float r_0_25 = fmaf(1.0f, r_1_9, dx * r_1_15);
-    const float r_1_25 = fmaf(1.0f, r_2_9, dx * r_2_15);
-    const float r_2_25 = fmaf(1.0f, r_3_9, dx * r_3_15);
-    const float r_0_26 = dx * r_1_16;
-    const float r_1_26 = dx * r_2_16;
-    const float r_2_26 = dx * r_3_16;
-    const float r_0_27 = dx * r_1_17;
-    const float r_1_27 = dx * r_2_17;
-    const float r_2_27 = dx * r_3_17;
-    const float r_0_28 = dx * r_1_18;
-    const float r_1_28 = dx * r_2_18;
-    const float r_2_28 = dx * r_3_18;
-    const float r_0_29 = dx * r_1_19;
-    const float r_1_29 = dx * r_2_19;
-    const float r_2_29 = dx * r_3_19;
-    const float r_0_30 = fmaf(3.0f, r_1_7, dy * r_1_16);
-    const float r_1_30 = fmaf(3.0f, r_2_7, dy * r_2_16);
-    const float r_2_30 = fmaf(3.0f, r_3_7, dy * r_3_16);
-    const float r_0_31 = fmaf(2.0f, r_1_8, dy * r_1_17);
-    const float r_1_31 = fmaf(2.0f, r_2_8, dy * r_2_17);
-    const float r_2_31 = fmaf(2.0f, r_3_8, dy * r_3_17);
-    const float r_0_32 = fmaf(1.0f, r_1_9, dy * r_1_18);
-    const float r_1_32 = fmaf(1.0f, r_2_9, dy * r_2_18);
-    const float r_2_32 = fmaf(1.0f, r_3_9, dy * r_3_18);
-    const float r_0_33 = dy * r_1_19;
-    const float r_1_33 = dy * r_2_19;
-    const float r_2_33 = dy * r_3_19;
-    const float r_0_34 = fmaf(3.0f, r_1_9, dz * r_1_19);
-    const float r_1_34 = fmaf(3.0f, r_2_9, dz * r_2_19);
-    const float r_2_34 = fmaf(3.0f, r_3_9, dz * r_3_19);
-    const float r_0_35 = fmaf(4.0f, r_1_10, dx * r_1_20);
-    const float r_1_35 = fmaf(4.0f, r_2_10, dx * r_2_20);
-    const float r_0_36 = fmaf(3.0f, r_1_11, dx * r_1_21);
-    const float r_1_36 = fmaf(3.0f, r_2_11, dx * r_2_21);
-    const float r_0_37 = fmaf(3.0f, r_1_12, dx * r_1_22);
-    const float r_1_37 = fmaf(3.0f, r_2_12, dx * r_2_22);
-    const float r_0_38 = fmaf(2.0f, r_1_13, dx * r_1_23);
-    const float r_1_38 = fmaf(2.0f, r_2_13, dx * r_2_23);
-    const float r_0_39 = fmaf(2.0f, r_1_14, dx * r_1_24);
-    const float r_1_39 = fmaf(2.0f, r_2_14, dx * r_2_24);
-    const float r_0_40 = fmaf(2.0f, r_1_15, dx * r_1_25);
-    const float r_1_40 = fmaf(2.0f, r_2_15, dx * r_2_25);
-    const float r_0_41 = fmaf(1.0f, r_1_16, dx * r_1_26);
-    const float r_1_41 = fmaf(1.0f, r_2_16, dx * r_2_26);
-    const float r_0_42 = fmaf(1.0f, r_1_17, dx * r_1_27);
-    const float r_1_42 = fmaf(1.0f, r_2_17, dx * r_2_27);
-    const float r_0_43 = fmaf(1.0f, r_1_18, dx * r_1_28);
-    const float r_1_43 = fmaf(1.0f, r_2_18, dx * r_2_28);
-    const float r_0_44 = fmaf(1.0f, r_1_19, dx * r_1_29);
-    const float r_1_44 = fmaf(1.0f, r_2_19, dx * r_2_29);
-    const float r_0_45 = dx * r_1_30;
-    const float r_1_45 = dx * r_2_30;
-    const float r_0_46 = dx * r_1_31;
-    const float r_1_46 = dx * r_2_31;
-    const float r_0_47 = dx * r_1_32;
-    const float r_1_47 = dx * r_2_32;
-    const float r_0_48 = dx * r_1_33;
-    const float r_1_48 = dx * r_2_33;
-    const float r_0_49 = dx * r_1_34;
-    const float r_1_49 = dx * r_2_34;
-    const float r_0_50 = fmaf(4.0f, r_1_16, dy * r_1_30);
-    const float r_1_50 = fmaf(4.0f, r_2_16, dy * r_2_30);
-    const float r_0_51 = fmaf(3.0f, r_1_17, dy * r_1_31);
-    const float r_1_51 = fmaf(3.0f, r_2_17, dy * r_2_31);
-    const float r_0_52 = fmaf(2.0f, r_1_18, dy * r_1_32);
-    const float r_1_52 = fmaf(2.0f, r_2_18, dy * r_2_32);
-    const float r_0_53 = fmaf(1.0f, r_1_19, dy * r_1_33);
-    const float r_1_53 = fmaf(1.0f, r_2_19, dy * r_2_33);
-    const float r_0_54 = dy * r_1_34;
-    const float r_1_54 = dy * r_2_34;
-    const float r_0_55 = fmaf(4.0f, r_1_19, dz * r_1_34);
-    const float r_1_55 = fmaf(4.0f, r_2_19, dz * r_2_34);
-    const float r_0_56 = fmaf(5.0f, r_1_20, dx * r_1_35);
-    const float r_0_57 = fmaf(4.0f, r_1_21, dx * r_1_36);
-    const float r_0_58 = fmaf(4.0f, r_1_22, dx * r_1_37);
-    const float r_0_59 = fmaf(3.0f, r_1_23, dx * r_1_38);
-    const float r_0_60 = fmaf(3.0f, r_1_24, dx * r_1_39);
-    const float r_0_61 = fmaf(3.0f, r_1_25, dx * r_1_40);
-    const float r_0_62 = fmaf(2.0f, r_1_26, dx * r_1_41);
-    const float r_0_63 = fmaf(2.0f, r_1_27, dx * r_1_42);
-    const float r_0_64 = fmaf(2.0f, r_1_28, dx * r_1_43);
-    const float r_0_65 = fmaf(2.0f, r_1_29, dx * r_1_44);
-    const float r_0_66 = fmaf(1.0f, r_1_30, dx * r_1_45);
-    const float r_0_67 = fmaf(1.0f, r_1_31, dx * r_1_46);
-    const float r_0_68 = fmaf(1.0f, r_1_32, dx * r_1_47);
-    const float r_0_69 = fmaf(1.0f, r_1_33, dx * r_1_48);
-    const float r_0_70 = fmaf(1.0f, r_1_34, dx * r_1_49);
-    const float r_0_71 = dx * r_1_50;
-    const float r_0_72 = dx * r_1_51;
-    const float r_0_73 = dx * r_1_52;
-    const float r_0_74 = dx * r_1_53;
-    const float r_0_75 = dx * r_1_54;
-    const float r_0_76 = dx * r_1_55;
-    const float r_0_77 = fmaf(5.0f, r_1_30, dy * r_1_50);
-    const float r_0_78 = fmaf(4.0f, r_1_31, dy * r_1_51);
-    const float r_0_79 = fmaf(3.0f, r_1_32, dy * r_1_52);
-    const float r_0_80 = fmaf(2.0f, r_1_33, dy * r_1_53);
-    const float r_0_81 = fmaf(1.0f, r_1_34, dy * r_1_54);
-    const float r_0_82 = dy * r_1_55;
-    const float r_0_83 = fmaf(5.0f, r_1_34, dz * r_1_55);
+    const T s2 = m2l_fma(dx, dx, m2l_fma(dy, dy, m2l_fma(dz, dz, soft2)));
+    const T si = m2l_rsqrt(s2);
+    const T si2 = si * si;
+    const T f0 = -si;
+    const T f1 = T(-1) * f0 * si2;
+    const T f2 = T(-3) * f1 * si2;
+    const T f3 = T(-5) * f2 * si2;
+    const T f4 = T(-7) * f3 * si2;
+    const T f5 = T(-9) * f4 * si2;
+    const T f6 = T(-11) * f5 * si2;
+    const T r_0_0 = f0;
+    const T r_1_0 = f1;
+    const T r_2_0 = f2;
+    const T r_3_0 = f3;
+    const T r_4_0 = f4;
+    const T r_5_0 = f5;
+    const T r_6_0 = f6;
+    const T r_0_1 = dx * r_1_0;
+    const T r_1_1 = dx * r_2_0;
+    const T r_2_1 = dx * r_3_0;
+    const T r_3_1 = dx * r_4_0;
+    const T r_4_1 = dx * r_5_0;
+    const T r_5_1 = dx * r_6_0;
+    const T r_0_2 = dy * r_1_0;
+    const T r_1_2 = dy * r_2_0;
+    const T r_2_2 = dy * r_3_0;
+    const T r_3_2 = dy * r_4_0;
+    const T r_4_2 = dy * r_5_0;
+    const T r_5_2 = dy * r_6_0;
+    const T r_0_3 = dz * r_1_0;
+    const T r_1_3 = dz * r_2_0;
+    const T r_2_3 = dz * r_3_0;
+    const T r_3_3 = dz * r_4_0;
+    const T r_4_3 = dz * r_5_0;
+    const T r_5_3 = dz * r_6_0;
+    const T r_0_4 = m2l_fma(T(1), r_1_0, dx * r_1_1);
+    const T r_1_4 = m2l_fma(T(1), r_2_0, dx * r_2_1);
+    const T r_2_4 = m2l_fma(T(1), r_3_0, dx * r_3_1);
+    const T r_3_4 = m2l_fma(T(1), r_4_0, dx * r_4_1);
+    const T r_4_4 = m2l_fma(T(1), r_5_0, dx * r_5_1);
+    const T r_0_5 = dx * r_1_2;
+    const T r_1_5 = dx * r_2_2;
+    const T r_2_5 = dx * r_3_2;
+    const T r_3_5 = dx * r_4_2;
+    const T r_4_5 = dx * r_5_2;
+    const T r_0_6 = dx * r_1_3;
+    const T r_1_6 = dx * r_2_3;
+    const T r_2_6 = dx * r_3_3;
+    const T r_3_6 = dx * r_4_3;
+    const T r_4_6 = dx * r_5_3;
+    const T r_0_7 = m2l_fma(T(1), r_1_0, dy * r_1_2);
+    const T r_1_7 = m2l_fma(T(1), r_2_0, dy * r_2_2);
+    const T r_2_7 = m2l_fma(T(1), r_3_0, dy * r_3_2);
+    const T r_3_7 = m2l_fma(T(1), r_4_0, dy * r_4_2);
+    const T r_4_7 = m2l_fma(T(1), r_5_0, dy * r_5_2);
+    const T r_0_8 = dy * r_1_3;
+    const T r_1_8 = dy * r_2_3;
+    const T r_2_8 = dy * r_3_3;
+    const T r_3_8 = dy * r_4_3;
+    const T r_4_8 = dy * r_5_3;
+    const T r_0_9 = m2l_fma(T(1), r_1_0, dz * r_1_3);
+    const T r_1_9 = m2l_fma(T(1), r_2_0, dz * r_2_3);
+    const T r_2_9 = m2l_fma(T(1), r_3_0, dz * r_3_3);
+    const T r_3_9 = m2l_fma(T(1), r_4_0, dz * r_4_3);
+    const T r_4_9 = m2l_fma(T(1), r_5_0, dz * r_5_3);
+    const T r_0_10 = m2l_fma(T(2), r_1_1, dx * r_1_4);
+    const T r_1_10 = m2l_fma(T(2), r_2_1, dx * r_2_4);
+    const T r_2_10 = m2l_fma(T(2), r_3_1, dx * r_3_4);
+    const T r_3_10 = m2l_fma(T(2), r_4_1, dx * r_4_4);
+    const T r_0_11 = m2l_fma(T(1), r_1_2, dx * r_1_5);
+    const T r_1_11 = m2l_fma(T(1), r_2_2, dx * r_2_5);
+    const T r_2_11 = m2l_fma(T(1), r_3_2, dx * r_3_5);
+    const T r_3_11 = m2l_fma(T(1), r_4_2, dx * r_4_5);
+    const T r_0_12 = m2l_fma(T(1), r_1_3, dx * r_1_6);
+    const T r_1_12 = m2l_fma(T(1), r_2_3, dx * r_2_6);
+    const T r_2_12 = m2l_fma(T(1), r_3_3, dx * r_3_6);
+    const T r_3_12 = m2l_fma(T(1), r_4_3, dx * r_4_6);
+    const T r_0_13 = dx * r_1_7;
+    const T r_1_13 = dx * r_2_7;
+    const T r_2_13 = dx * r_3_7;
+    const T r_3_13 = dx * r_4_7;
+    const T r_0_14 = dx * r_1_8;
+    const T r_1_14 = dx * r_2_8;
+    const T r_2_14 = dx * r_3_8;
+    const T r_3_14 = dx * r_4_8;
+    const T r_0_15 = dx * r_1_9;
+    const T r_1_15 = dx * r_2_9;
+    const T r_2_15 = dx * r_3_9;
+    const T r_3_15 = dx * r_4_9;
+    const T r_0_16 = m2l_fma(T(2), r_1_2, dy * r_1_7);
+    const T r_1_16 = m2l_fma(T(2), r_2_2, dy * r_2_7);
+    const T r_2_16 = m2l_fma(T(2), r_3_2, dy * r_3_7);
+    const T r_3_16 = m2l_fma(T(2), r_4_2, dy * r_4_7);
+    const T r_0_17 = m2l_fma(T(1), r_1_3, dy * r_1_8);
+    const T r_1_17 = m2l_fma(T(1), r_2_3, dy * r_2_8);
+    const T r_2_17 = m2l_fma(T(1), r_3_3, dy * r_3_8);
+    const T r_3_17 = m2l_fma(T(1), r_4_3, dy * r_4_8);
+    const T r_0_18 = dy * r_1_9;
+    const T r_1_18 = dy * r_2_9;
+    const T r_2_18 = dy * r_3_9;
+    const T r_3_18 = dy * r_4_9;
+    const T r_0_19 = m2l_fma(T(2), r_1_3, dz * r_1_9);
+    const T r_1_19 = m2l_fma(T(2), r_2_3, dz * r_2_9);
+    const T r_2_19 = m2l_fma(T(2), r_3_3, dz * r_3_9);
+    const T r_3_19 = m2l_fma(T(2), r_4_3, dz * r_4_9);
+    const T r_0_20 = m2l_fma(T(3), r_1_4, dx * r_1_10);
+    const T r_1_20 = m2l_fma(T(3), r_2_4, dx * r_2_10);
+    const T r_2_20 = m2l_fma(T(3), r_3_4, dx * r_3_10);
+    const T r_0_21 = m2l_fma(T(2), r_1_5, dx * r_1_11);
+    const T r_1_21 = m2l_fma(T(2), r_2_5, dx * r_2_11);
+    const T r_2_21 = m2l_fma(T(2), r_3_5, dx * r_3_11);
+    const T r_0_22 = m2l_fma(T(2), r_1_6, dx * r_1_12);
+    const T r_1_22 = m2l_fma(T(2), r_2_6, dx * r_2_12);
+    const T r_2_22 = m2l_fma(T(2), r_3_6, dx * r_3_12);
+    const T r_0_23 = m2l_fma(T(1), r_1_7, dx * r_1_13);
+    const T r_1_23 = m2l_fma(T(1), r_2_7, dx * r_2_13);
+    const T r_2_23 = m2l_fma(T(1), r_3_7, dx * r_3_13);
+    const T r_0_24 = m2l_fma(T(1), r_1_8, dx * r_1_14);
+    const T r_1_24 = m2l_fma(T(1), r_2_8, dx * r_2_14);
+    const T r_2_24 = m2l_fma(T(1), r_3_8, dx * r_3_14);
+    const T r_0_25 = m2l_fma(T(1), r_1_9, dx * r_1_15);
+    const T r_1_25 = m2l_fma(T(1), r_2_9, dx * r_2_15);
+    const T r_2_25 = m2l_fma(T(1), r_3_9, dx * r_3_15);
+    const T r_0_26 = dx * r_1_16;
+    const T r_1_26 = dx * r_2_16;
+    const T r_2_26 = dx * r_3_16;
+    const T r_0_27 = dx * r_1_17;
+    const T r_1_27 = dx * r_2_17;
+    const T r_2_27 = dx * r_3_17;
+    const T r_0_28 = dx * r_1_18;
+    const T r_1_28 = dx * r_2_18;
+    const T r_2_28 = dx * r_3_18;
+    const T r_0_29 = dx * r_1_19;
+    const T r_1_29 = dx * r_2_19;
+    const T r_2_29 = dx * r_3_19;
+    const T r_0_30 = m2l_fma(T(3), r_1_7, dy * r_1_16);
+    const T r_1_30 = m2l_fma(T(3), r_2_7, dy * r_2_16);
+    const T r_2_30 = m2l_fma(T(3), r_3_7, dy * r_3_16);
+    const T r_0_31 = m2l_fma(T(2), r_1_8, dy * r_1_17);
+    const T r_1_31 = m2l_fma(T(2), r_2_8, dy * r_2_17);
+    const T r_2_31 = m2l_fma(T(2), r_3_8, dy * r_3_17);
+    const T r_0_32 = m2l_fma(T(1), r_1_9, dy * r_1_18);
+    const T r_1_32 = m2l_fma(T(1), r_2_9, dy * r_2_18);
+    const T r_2_32 = m2l_fma(T(1), r_3_9, dy * r_3_18);
+    const T r_0_33 = dy * r_1_19;
+    const T r_1_33 = dy * r_2_19;
+    const T r_2_33 = dy * r_3_19;
+    const T r_0_34 = m2l_fma(T(3), r_1_9, dz * r_1_19);
+    const T r_1_34 = m2l_fma(T(3), r_2_9, dz * r_2_19);
+    const T r_2_34 = m2l_fma(T(3), r_3_9, dz * r_3_19);
+    const T r_0_35 = m2l_fma(T(4), r_1_10, dx * r_1_20);
+    const T r_1_35 = m2l_fma(T(4), r_2_10, dx * r_2_20);
+    const T r_0_36 = m2l_fma(T(3), r_1_11, dx * r_1_21);
+    const T r_1_36 = m2l_fma(T(3), r_2_11, dx * r_2_21);
+    const T r_0_37 = m2l_fma(T(3), r_1_12, dx * r_1_22);
+    const T r_1_37 = m2l_fma(T(3), r_2_12, dx * r_2_22);
+    const T r_0_38 = m2l_fma(T(2), r_1_13, dx * r_1_23);
+    const T r_1_38 = m2l_fma(T(2), r_2_13, dx * r_2_23);
+    const T r_0_39 = m2l_fma(T(2), r_1_14, dx * r_1_24);
+    const T r_1_39 = m2l_fma(T(2), r_2_14, dx * r_2_24);
+    const T r_0_40 = m2l_fma(T(2), r_1_15, dx * r_1_25);
+    const T r_1_40 = m2l_fma(T(2), r_2_15, dx * r_2_25);
+    const T r_0_41 = m2l_fma(T(1), r_1_16, dx * r_1_26);
+    const T r_1_41 = m2l_fma(T(1), r_2_16, dx * r_2_26);
+    const T r_0_42 = m2l_fma(T(1), r_1_17, dx * r_1_27);
+    const T r_1_42 = m2l_fma(T(1), r_2_17, dx * r_2_27);
+    const T r_0_43 = m2l_fma(T(1), r_1_18, dx * r_1_28);
+    const T r_1_43 = m2l_fma(T(1), r_2_18, dx * r_2_28);
+    const T r_0_44 = m2l_fma(T(1), r_1_19, dx * r_1_29);
+    const T r_1_44 = m2l_fma(T(1), r_2_19, dx * r_2_29);
+    const T r_0_45 = dx * r_1_30;
+    const T r_1_45 = dx * r_2_30;
+    const T r_0_46 = dx * r_1_31;
+    const T r_1_46 = dx * r_2_31;
+    const T r_0_47 = dx * r_1_32;
+    const T r_1_47 = dx * r_2_32;
+    const T r_0_48 = dx * r_1_33;
+    const T r_1_48 = dx * r_2_33;
+    const T r_0_49 = dx * r_1_34;
+    const T r_1_49 = dx * r_2_34;
+    const T r_0_50 = m2l_fma(T(4), r_1_16, dy * r_1_30);
+    const T r_1_50 = m2l_fma(T(4), r_2_16, dy * r_2_30);
+    const T r_0_51 = m2l_fma(T(3), r_1_17, dy * r_1_31);
+    const T r_1_51 = m2l_fma(T(3), r_2_17, dy * r_2_31);
+    const T r_0_52 = m2l_fma(T(2), r_1_18, dy * r_1_32);
+    const T r_1_52 = m2l_fma(T(2), r_2_18, dy * r_2_32);
+    const T r_0_53 = m2l_fma(T(1), r_1_19, dy * r_1_33);
+    const T r_1_53 = m2l_fma(T(1), r_2_19, dy * r_2_33);
+    const T r_0_54 = dy * r_1_34;
+    const T r_1_54 = dy * r_2_34;
+    const T r_0_55 = m2l_fma(T(4), r_1_19, dz * r_1_34);
+    const T r_1_55 = m2l_fma(T(4), r_2_19, dz * r_2_34);
+    const T r_0_56 = m2l_fma(T(5), r_1_20, dx * r_1_35);
+    const T r_0_57 = m2l_fma(T(4), r_1_21, dx * r_1_36);
+    const T r_0_58 = m2l_fma(T(4), r_1_22, dx * r_1_37);
+    const T r_0_59 = m2l_fma(T(3), r_1_23, dx * r_1_38);
+    const T r_0_60 = m2l_fma(T(3), r_1_24, dx * r_1_39);
+    const T r_0_61 = m2l_fma(T(3), r_1_25, dx * r_1_40);
+    const T r_0_62 = m2l_fma(T(2), r_1_26, dx * r_1_41);
+    const T r_0_63 = m2l_fma(T(2), r_1_27, dx * r_1_42);
+    const T r_0_64 = m2l_fma(T(2), r_1_28, dx * r_1_43);
+    const T r_0_65 = m2l_fma(T(2), r_1_29, dx * r_1_44);
+    const T r_0_66 = m2l_fma(T(1), r_1_30, dx * r_1_45);
+    const T r_0_67 = m2l_fma(T(1), r_1_31, dx * r_1_46);
+    const T r_0_68 = m2l_fma(T(1), r_1_32, dx * r_1_47);
+    const T r_0_69 = m2l_fma(T(1), r_1_33, dx * r_1_48);
+    const T r_0_70 = m2l_fma(T(1), r_1_34, dx * r_1_49);
+    const T r_0_71 = dx * r_1_50;
+    const T r_0_72 = dx * r_1_51;
+    const T r_0_73 = dx * r_1_52;
+    const T r_0_74 = dx * r_1_53;
+    const T r_0_75 = dx * r_1_54;
+    const T r_0_76 = dx * r_1_55;
+    const T r_0_77 = m2l_fma(T(5), r_1_30, dy * r_1_50);
+    const T r_0_78 = m2l_fma(T(4), r_1_31, dy * r_1_51);
+    const T r_0_79 = m2l_fma(T(3), r_1_32, dy * r_1_52);
+    const T r_0_80 = m2l_fma(T(2), r_1_33, dy * r_1_53);
+    const T r_0_81 = m2l_fma(T(1), r_1_34, dy * r_1_54);
+    const T r_0_82 = dy * r_1_55;
+    const T r_0_83 = m2l_fma(T(5), r_1_34, dz * r_1_55);
     D[0] = r_0_0;
     D[1] = r_0_1;
     D[2] = r_0_2;
@@ -4565,10 +4570,10 @@ __device__ __forceinline__ void m2l_dtensor_6(float dx, float dy, float dz, floa
     D[83] = r_0_83;
 }
 
-__device__ __forceinline__ void m2l_side_a_6(const float (&D)[84], const float *__restrict__ Ms, float rho, float (&L)[84])
+template <class T> __device__ __forceinline__ void m2l_side_a_6(const T (&D)[84], const T *__restrict__ Ms, T rho, T (&L)[84])
 {
-    float rp = 1.0f;
-    { const float m = __ldg(Ms + 0) * rp;
+    T rp = T(1);
+    { const T m = __ldg(Ms + 0) * rp;
       L[0] = D[0] * m;
       L[1] = D[1] * m;
       L[2] = D[2] * m;
@@ -4655,1022 +4660,1022 @@ __device__ __forceinline__ void m2l_side_a_6(const float (&D)[84], const float *
       L[83] = D[83] * m;
     }
     rp *= rho;
-    { const float m = -__ldg(Ms + 1) * rp;
-      L[0] = fmaf(D[1], m, L[0]);
-      L[1] = fmaf(D[4], m, L[1]);
-      L[2] = fmaf(D[5], m, L[2]);
-      L[3] = fmaf(D[6], m, L[3]);
-      L[4] = fmaf(D[10], m, L[4]);
-      L[5] = fmaf(D[11], m, L[5]);
-      L[6] = fmaf(D[12], m, L[6]);
-      L[7] = fmaf(D[13], m, L[7]);
-      L[8] = fmaf(D[14], m, L[8]);
-      L[9] = fmaf(D[15], m, L[9]);
-      L[10] = fmaf(D[20], m, L[10]);
-      L[11] = fmaf(D[21], m, L[11]);
-      L[12] = fmaf(D[22], m, L[12]);
-      L[13] = fmaf(D[23], m, L[13]);
-      L[14] = fmaf(D[24], m, L[14]);
-      L[15] = fmaf(D[25], m, L[15]);
-      L[16] = fmaf(D[26], m, L[16]);
-      L[17] = fmaf(D[27], m, L[17]);
-      L[18] = fmaf(D[28], m, L[18]);
-      L[19] = fmaf(D[29], m, L[19]);
-      L[20] = fmaf(D[35], m, L[20]);
-      L[21] = fmaf(D[36], m, L[21]);
-      L[22] = fmaf(D[37], m, L[22]);
-      L[23] = fmaf(D[38], m, L[23]);
-      L[24] = fmaf(D[39], m, L[24]);
-      L[25] = fmaf(D[40], m, L[25]);
-      L[26] = fmaf(D[41], m, L[26]);
-      L[27] = fmaf(D[42], m, L[27]);
-      L[28] = fmaf(D[43], m, L[28]);
-      L[29] = fmaf(D[44], m, L[29]);
-      L[30] = fmaf(D[45], m, L[30]);
-      L[31] = fmaf(D[46], m, L[31]);
-      L[32] = fmaf(D[47], m, L[32]);
-      L[33] = fmaf(D[48], m, L[33]);
-      L[34] = fmaf(D[49], m, L[34]);
-      L[35] = fmaf(D[56], m, L[35]);
-      L[36] = fmaf(D[57], m, L[36]);
-      L[37] = fmaf(D[58], m, L[37]);
-      L[38] = fmaf(D[59], m, L[38]);
-      L[39] = fmaf(D[60], m, L[39]);
-      L[40] = fmaf(D[61], m, L[40]);
-      L[41] = fmaf(D[62], m, L[41]);
-      L[42] = fmaf(D[63], m, L[42]);
-      L[43] = fmaf(D[64], m, L[43]);
-      L[44] = fmaf(D[65], m, L[44]);
-      L[45] = fmaf(D[66], m, L[45]);
-      L[46] = fmaf(D[67], m, L[46]);
-      L[47] = fmaf(D[68], m, L[47]);
-      L[48] = fmaf(D[69], m, L[48]);
-      L[49] = fmaf(D[70], m, L[49]);
-      L[50] = fmaf(D[71], m, L[50]);
-      L[51] = fmaf(D[72], m, L[51]);
-      L[52] = fmaf(D[73], m, L[52]);
-      L[53] = fmaf(D[74], m, L[53]);
-      L[54] = fmaf(D[75], m, L[54]);
-      L[55] = fmaf(D[76], m, L[55]);
+    { const T m = -__ldg(Ms + 1) * rp;
+      L[0] = m2l_fma(D[1], m, L[0]);
+      L[1] = m2l_fma(D[4], m, L[1]);
+      L[2] = m2l_fma(D[5], m, L[2]);
+      L[3] = m2l_fma(D[6], m, L[3]);
+      L[4] = m2l_fma(D[10], m, L[4]);
+      L[5] = m2l_fma(D[11], m, L[5]);
+      L[6] = m2l_fma(D[12], m, L[6]);
+      L[7] = m2l_fma(D[13], m, L[7]);
+      L[8] = m2l_fma(D[14], m, L[8]);
+      L[9] = m2l_fma(D[15], m, L[9]);
+      L[10] = m2l_fma(D[20], m, L[10]);
+      L[11] = m2l_fma(D[21], m, L[11]);
+      L[12] = m2l_fma(D[22], m, L[12]);
+      L[13] = m2l_fma(D[23], m, L[13]);
+      L[14] = m2l_fma(D[24], m, L[14]);
+      L[15] = m2l_fma(D[25], m, L[15]);
+      L[16] = m2l_fma(D[26], m, L[16]);
+      L[17] = m2l_fma(D[27], m, L[17]);
+      L[18] = m2l_fma(D[28], m, L[18]);
+      L[19] = m2l_fma(D[29], m, L[19]);
+      L[20] = m2l_fma(D[35], m, L[20]);
+      L[21] = m2l_fma(D[36], m, L[21]);
+      L[22] = m2l_fma(D[37], m, L[22]);
+      L[23] = m2l_fma(D[38], m, L[23]);
+      L[24] = m2l_fma(D[39], m, L[24]);
+      L[25] = m2l_fma(D[40], m, L[25]);
+      L[26] = m2l_fma(D[41], m, L[26]);
+      L[27] = m2l_fma(D[42], m, L[27]);
+      L[28] = m2l_fma(D[43], m, L[28]);
+      L[29] = m2l_fma(D[44], m, L[29]);
+      L[30] = m2l_fma(D[45], m, L[30]);
+      L[31] = m2l_fma(D[46], m, L[31]);
+      L[32] = m2l_fma(D[47], m, L[32]);
+      L[33] = m2l_fma(D[48], m, L[33]);
+      L[34] = m2l_fma(D[49], m, L[34]);
+      L[35] = m2l_fma(D[56], m, L[35]);
+      L[36] = m2l_fma(D[57], m, L[36]);
+      L[37] = m2l_fma(D[58], m, L[37]);
+      L[38] = m2l_fma(D[59], m, L[38]);
+      L[39] = m2l_fma(D[60], m, L[39]);
+      L[40] = m2l_fma(D[61], m, L[40]);
+      L[41] = m2l_fma(D[62], m, L[41]);
+      L[42] = m2l_fma(D[63], m, L[42]);
+      L[43] = m2l_fma(D[64], m, L[43]);
+      L[44] = m2l_fma(D[65], m, L[44]);
+      L[45] = m2l_fma(D[66], m, L[45]);
+      L[46] = m2l_fma(D[67], m, L[46]);
+      L[47] = m2l_fma(D[68], m, L[47]);
+      L[48] = m2l_fma(D[69], m, L[48]);
+      L[49] = m2l_fma(D[70], m, L[49]);
+      L[50] = m2l_fma(D[71], m, L[50]);
+      L[51] = m2l_fma(D[72], m, L[51]);
+      L[52] = m2l_fma(D[73], m, L[52]);
+      L[53] = m2l_fma(D[74], m, L[53]);
+      L[54] = m2l_fma(D[75], m, L[54]);
+      L[55] = m2l_fma(D[76], m, L[55]);
     }
-    { const float m = -__ldg(Ms + 2) * rp;
-      L[0] = fmaf(D[2], m, L[0]);
-      L[1] = fmaf(D[5], m, L[1]);
-      L[2] = fmaf(D[7], m, L[2]);
-      L[3] = fmaf(D[8], m, L[3]);
-      L[4] = fmaf(D[11], m, L[4]);
-      L[5] = fmaf(D[13], m, L[5]);
-      L[6] = fmaf(D[14], m, L[6]);
-      L[7] = fmaf(D[16], m, L[7]);
-      L[8] = fmaf(D[17], m, L[8]);
-      L[9] = fmaf(D[18], m, L[9]);
-      L[10] = fmaf(D[21], m, L[10]);
-      L[11] = fmaf(D[23], m, L[11]);
-      L[12] = fmaf(D[24], m, L[12]);
-      L[13] = fmaf(D[26], m, L[13]);
-      L[14] = fmaf(D[27], m, L[14]);
-      L[15] = fmaf(D[28], m, L[15]);
-      L[16] = fmaf(D[30], m, L[16]);
-      L[17] = fmaf(D[31], m, L[17]);
-      L[18] = fmaf(D[32], m, L[18]);
-      L[19] = fmaf(D[33], m, L[19]);
-      L[20] = fmaf(D[36], m, L[20]);
-      L[21] = fmaf(D[38], m, L[21]);
-      L[22] = fmaf(D[39], m, L[22]);
-      L[23] = fmaf(D[41], m, L[23]);
-      L[24] = fmaf(D[42], m, L[24]);
-      L[25] = fmaf(D[43], m, L[25]);
-      L[26] = fmaf(D[45], m, L[26]);
-      L[27] = fmaf(D[46], m, L[27]);
-      L[28] = fmaf(D[47], m, L[28]);
-      L[29] = fmaf(D[48], m, L[29]);
-      L[30] = fmaf(D[50], m, L[30]);
-      L[31] = fmaf(D[51], m, L[31]);
-      L[32] = fmaf(D[52], m, L[32]);
-      L[33] = fmaf(D[53], m, L[33]);
-      L[34] = fmaf(D[54], m, L[34]);
-      L[35] = fmaf(D[57], m, L[35]);
-      L[36] = fmaf(D[59], m, L[36]);
-      L[37] = fmaf(D[60], m, L[37]);
-      L[38] = fmaf(D[62], m, L[38]);
-      L[39] = fmaf(D[63], m, L[39]);
-      L[40] = fmaf(D[64], m, L[40]);
-      L[41] = fmaf(D[66], m, L[41]);
-      L[42] = fmaf(D[67], m, L[42]);
-      L[43] = fmaf(D[68], m, L[43]);
-      L[44] = fmaf(D[69], m, L[44]);
-      L[45] = fmaf(D[71], m, L[45]);
-      L[46] = fmaf(D[72], m, L[46]);
-      L[47] = fmaf(D[73], m, L[47]);
-      L[48] = fmaf(D[74], m, L[48]);
-      L[49] = fmaf(D[75], m, L[49]);
-      L[50] = fmaf(D[77], m, L[50]);
-      L[51] = fmaf(D[78], m, L[51]);
-      L[52] = fmaf(D[79], m, L[52]);
-      L[53] = fmaf(D[80], m, L[53]);
-      L[54] = fmaf(D[81], m, L[54]);
-      L[55] = fmaf(D[82], m, L[55]);
+    { const T m = -__ldg(Ms + 2) * rp;
+      L[0] = m2l_fma(D[2], m, L[0]);
+      L[1] = m2l_fma(D[5], m, L[1]);
+      L[2] = m2l_fma(D[7], m, L[2]);
+      L[3] = m2l_fma(D[8], m, L[3]);
+      L[4] = m2l_fma(D[11], m, L[4]);
+      L[5] = m2l_fma(D[13], m, L[5]);
+      L[6] = m2l_fma(D[14], m, L[6]);
+      L[7] = m2l_fma(D[16], m, L[7]);
+      L[8] = m2l_fma(D[17], m, L[8]);
+      L[9] = m2l_fma(D[18], m, L[9]);
+      L[10] = m2l_fma(D[21], m, L[10]);
+      L[11] = m2l_fma(D[23], m, L[11]);
+      L[12] = m2l_fma(D[24], m, L[12]);
+      L[13] = m2l_fma(D[26], m, L[13]);
+      L[14] = m2l_fma(D[27], m, L[14]);
+      L[15] = m2l_fma(D[28], m, L[15]);
+      L[16] = m2l_fma(D[30], m, L[16]);
+      L[17] = m2l_fma(D[31], m, L[17]);
+      L[18] = m2l_fma(D[32], m, L[18]);
+      L[19] = m2l_fma(D[33], m, L[19]);
+      L[20] = m2l_fma(D[36], m, L[20]);
+      L[21] = m2l_fma(D[38], m, L[21]);
+      L[22] = m2l_fma(D[39], m, L[22]);
+      L[23] = m2l_fma(D[41], m, L[23]);
+      L[24] = m2l_fma(D[42], m, L[24]);
+      L[25] = m2l_fma(D[43], m, L[25]);
+      L[26] = m2l_fma(D[45], m, L[26]);
+      L[27] = m2l_fma(D[46], m, L[27]);
+      L[28] = m2l_fma(D[47], m, L[28]);
+      L[29] = m2l_fma(D[48], m, L[29]);
+      L[30] = m2l_fma(D[50], m, L[30]);
+      L[31] = m2l_fma(D[51], m, L[31]);
+      L[32] = m2l_fma(D[52], m, L[32]);
+      L[33] = m2l_fma(D[53], m, L[33]);
+      L[34] = m2l_fma(D[54], m, L[34]);
+      L[35] = m2l_fma(D[57], m, L[35]);
+      L[36] = m2l_fma(D[59], m, L[36]);
+      L[37] = m2l_fma(D[60], m, L[37]);
+      L[38] = m2l_fma(D[62], m, L[38]);
+      L[39] = m2l_fma(D[63], m, L[39]);
+      L[40] = m2l_fma(D[64], m, L[40]);
+      L[41] = m2l_fma(D[66], m, L[41]);
+      L[42] = m2l_fma(D[67], m, L[42]);
+      L[43] = m2l_fma(D[68], m, L[43]);
+      L[44] = m2l_fma(D[69], m, L[44]);
+      L[45] = m2l_fma(D[71], m, L[45]);
+      L[46] = m2l_fma(D[72], m, L[46]);
+      L[47] = m2l_fma(D[73], m, L[47]);
+      L[48] = m2l_fma(D[74], m, L[48]);
+      L[49] = m2l_fma(D[75], m, L[49]);
+      L[50] = m2l_fma(D[77], m, L[50]);
+      L[51] = m2l_fma(D[78], m, L[51]);
+      L[52] = m2l_fma(D[79], m, L[52]);
+      L[53] = m2l_fma(D[80], m, L[53]);
+      L[54] = m2l_fma(D[81], m, L[54]);
+      L[55] = m2l_fma(D[82], m, L[55]);
     }
-    { const float m = -__ldg(Ms + 3) * rp;
-      L[0] = fmaf(D[3], m, L[0]);
-      L[1] = fmaf(D[6], m, L[1]);
-      L[2] = fmaf(D[8], m, L[2]);
-      L[3] = fmaf(D[9], m, L[3]);
-      L[4] = fmaf(D[12], m, L[4]);
-      L[5] = fmaf(D[14], m, L[5]);
-      L[6] = fmaf(D[15], m, L[6]);
-      L[7] = fmaf(D[17], m, L[7]);
-      L[8] = fmaf(D[18], m, L[8]);
-      L[9] = fmaf(D[19], m, L[9]);
-      L[10] = fmaf(D[22], m, L[10]);
-      L[11] = fmaf(D[24], m, L[11]);
-      L[12] = fmaf(D[25], m, L[12]);
-      L[13] = fmaf(D[27], m, L[13]);
-      L[14] = fmaf(D[28], m, L[14]);
-      L[15] = fmaf(D[29], m, L[15]);
-      L[16] = fmaf(D[31], m, L[16]);
-      L[17] = fmaf(D[32], m, L[17]);
-      L[18] = fmaf(D[33], m, L[18]);
-      L[19] = fmaf(D[34], m, L[19]);
-      L[20] = fmaf(D[37], m, L[20]);
-      L[21] = fmaf(D[39], m, L[21]);
-      L[22] = fmaf(D[40], m, L[22]);
-      L[23] = fmaf(D[42], m, L[23]);
-      L[24] = fmaf(D[43], m, L[24]);
-      L[25] = fmaf(D[44], m, L[25]);
-      L[26] = fmaf(D[46], m, L[26]);
-      L[27] = fmaf(D[47], m, L[27]);
-      L[28] = fmaf(D[48], m, L[28]);
-      L[29] = fmaf(D[49], m, L[29]);
-      L[30] = fmaf(D[51], m, L[30]);
-      L[31] = fmaf(D[52], m, L[31]);
-      L[32] = fmaf(D[53], m, L[32]);
-      L[33] = fmaf(D[54], m, L[33]);
-      L[34] = fmaf(D[55], m, L[34]);
-      L[35] = fmaf(D[58], m, L[35]);
-      L[36] = fmaf(D[60], m, L[36]);
-      L[37] = fmaf(D[61], m, L[37]);
-      L[38] = fmaf(D[63], m, L[38]);
-      L[39] = fmaf(D[64], m, L[39]);
-      L[40] = fmaf(D[65], m, L[40]);
-      L[41] = fmaf(D[67], m, L[41]);
-      L[42] = fmaf(D[68], m, L[42]);
-      L[43] = fmaf(D[69], m, L[43]);
-      L[44] = fmaf(D[70], m, L[44]);
-      L[45] = fmaf(D[72], m, L[45]);
-      L[46] = fmaf(D[73], m, L[46]);
-      L[47] = fmaf(D[74], m, L[47]);
-      L[48] = fmaf(D[75], m, L[48]);
-      L[49] = fmaf(D[76], m, L[49]);
-      L[50] = fmaf(D[78], m, L[50]);
-      L[51] = fmaf(D[79], m, L[51]);
-      L[52] = fmaf(D[80], m, L[52]);
-      L[53] = fmaf(D[81], m, L[53]);
-      L[54] = fmaf(D[82], m, L[54]);
-      L[55] = fmaf(D[83], m, L[55]);
-    }
-    rp *= rho;
-    { const float m = __ldg(Ms + 4) * rp;
-      L[0] = fmaf(D[4], m, L[0]);
-      L[1] = fmaf(D[10], m, L[1]);
-      L[2] = fmaf(D[11], m, L[2]);
-      L[3] = fmaf(D[12], m, L[3]);
-      L[4] = fmaf(D[20], m, L[4]);
-      L[5] = fmaf(D[21], m, L[5]);
-      L[6] = fmaf(D[22], m, L[6]);
-      L[7] = fmaf(D[23], m, L[7]);
-      L[8] = fmaf(D[24], m, L[8]);
-      L[9] = fmaf(D[25], m, L[9]);
-      L[10] = fmaf(D[35], m, L[10]);
-      L[11] = fmaf(D[36], m, L[11]);
-      L[12] = fmaf(D[37], m, L[12]);
-      L[13] = fmaf(D[38], m, L[13]);
-      L[14] = fmaf(D[39], m, L[14]);
-      L[15] = fmaf(D[40], m, L[15]);
-      L[16] = fmaf(D[41], m, L[16]);
-      L[17] = fmaf(D[42], m, L[17]);
-      L[18] = fmaf(D[43], m, L[18]);
-      L[19] = fmaf(D[44], m, L[19]);
-      L[20] = fmaf(D[56], m, L[20]);
-      L[21] = fmaf(D[57], m, L[21]);
-      L[22] = fmaf(D[58], m, L[22]);
-      L[23] = fmaf(D[59], m, L[23]);
-      L[24] = fmaf(D[60], m, L[24]);
-      L[25] = fmaf(D[61], m, L[25]);
-      L[26] = fmaf(D[62], m, L[26]);
-      L[27] = fmaf(D[63], m, L[27]);
-      L[28] = fmaf(D[64], m, L[28]);
-      L[29] = fmaf(D[65], m, L[29]);
-      L[30] = fmaf(D[66], m, L[30]);
-      L[31] = fmaf(D[67], m, L[31]);
-      L[32] = fmaf(D[68], m, L[32]);
-      L[33] = fmaf(D[69], m, L[33]);
-      L[34] = fmaf(D[70], m, L[34]);
-    }
-    { const float m = __ldg(Ms + 5) * rp;
-      L[0] = fmaf(D[5], m, L[0]);
-      L[1] = fmaf(D[11], m, L[1]);
-      L[2] = fmaf(D[13], m, L[2]);
-      L[3] = fmaf(D[14], m, L[3]);
-      L[4] = fmaf(D[21], m, L[4]);
-      L[5] = fmaf(D[23], m, L[5]);
-      L[6] = fmaf(D[24], m, L[6]);
-      L[7] = fmaf(D[26], m, L[7]);
-      L[8] = fmaf(D[27], m, L[8]);
-      L[9] = fmaf(D[28], m, L[9]);
-      L[10] = fmaf(D[36], m, L[10]);
-      L[11] = fmaf(D[38], m, L[11]);
-      L[12] = fmaf(D[39], m, L[12]);
-      L[13] = fmaf(D[41], m, L[13]);
-      L[14] = fmaf(D[42], m, L[14]);
-      L[15] = fmaf(D[43], m, L[15]);
-      L[16] = fmaf(D[45], m, L[16]);
-      L[17] = fmaf(D[46], m, L[17]);
-      L[18] = fmaf(D[47], m, L[18]);
-      L[19] = fmaf(D[48], m, L[19]);
-      L[20] = fmaf(D[57], m, L[20]);
-      L[21] = fmaf(D[59], m, L[21]);
-      L[22] = fmaf(D[60], m, L[22]);
-      L[23] = fmaf(D[62], m, L[23]);
-      L[24] = fmaf(D[63], m, L[24]);
-      L[25] = fmaf(D[64], m, L[25]);
-      L[26] = fmaf(D[66], m, L[26]);
-      L[27] = fmaf(D[67], m, L[27]);
-      L[28] = fmaf(D[68], m, L[28]);
-      L[29] = fmaf(D[69], m, L[29]);
-      L[30] = fmaf(D[71], m, L[30]);
-      L[31] = fmaf(D[72], m, L[31]);
-      L[32] = fmaf(D[73], m, L[32]);
-      L[33] = fmaf(D[74], m, L[33]);
-      L[34] = fmaf(D[75], m, L[34]);
-    }
-    { const float m = __ldg(Ms + 6) * rp;
-      L[0] = fmaf(D[6], m, L[0]);
-      L[1] = fmaf(D[12], m, L[1]);
-      L[2] = fmaf(D[14], m, L[2]);
-      L[3] = fmaf(D[15], m, L[3]);
-      L[4] = fmaf(D[22], m, L[4]);
-      L[5] = fmaf(D[24], m, L[5]);
-      L[6] = fmaf(D[25], m, L[6]);
-      L[7] = fmaf(D[27], m, L[7]);
-      L[8] = fmaf(D[28], m, L[8]);
-      L[9] = fmaf(D[29], m, L[9]);
-      L[10] = fmaf(D[37], m, L[10]);
-      L[11] = fmaf(D[39], m, L[11]);
-      L[12] = fmaf(D[40], m, L[12]);
-      L[13] = fmaf(D[42], m, L[13]);
-      L[14] = fmaf(D[43], m, L[14]);
-      L[15] = fmaf(D[44], m, L[15]);
-      L[16] = fmaf(D[46], m, L[16]);
-      L[17] = fmaf(D[47], m, L[17]);
-      L[18] = fmaf(D[48], m, L[18]);
-      L[19] = fmaf(D[49], m, L[19]);
-      L[20] = fmaf(D[58], m, L[20]);
-      L[21] = fmaf(D[60], m, L[21]);
-      L[22] = fmaf(D[61], m, L[22]);
-      L[23] = fmaf(D[63], m, L[23]);
-      L[24] = fmaf(D[64], m, L[24]);
-      L[25] = fmaf(D[65], m, L[25]);
-      L[26] = fmaf(D[67], m, L[26]);
-      L[27] = fmaf(D[68], m, L[27]);
-      L[28] = fmaf(D[69], m, L[28]);
-      L[29] = fmaf(D[70], m, L[29]);
-      L[30] = fmaf(D[72], m, L[30]);
-      L[31] = fmaf(D[73], m, L[31]);
-      L[32] = fmaf(D[74], m, L[32]);
-      L[33] = fmaf(D[75], m, L[33]);
-      L[34] = fmaf(D[76], m, L[34]);
-    }
-    { const float m = __ldg(Ms + 7) * rp;
-      L[0] = fmaf(D[7], m, L[0]);
-      L[1] = fmaf(D[13], m, L[1]);
-      L[2] = fmaf(D[16], m, L[2]);
-      L[3] = fmaf(D[17], m, L[3]);
-      L[4] = fmaf(D[23], m, L[4]);
-      L[5] = fmaf(D[26], m, L[5]);
-      L[6] = fmaf(D[27], m, L[6]);
-      L[7] = fmaf(D[30], m, L[7]);
-      L[8] = fmaf(D[31], m, L[8]);
-      L[9] = fmaf(D[32], m, L[9]);
-      L[10] = fmaf(D[38], m, L[10]);
-      L[11] = fmaf(D[41], m, L[11]);
-      L[12] = fmaf(D[42], m, L[12]);
-      L[13] = fmaf(D[45], m, L[13]);
-      L[14] = fmaf(D[46], m, L[14]);
-      L[15] = fmaf(D[47], m, L[15]);
-      L[16] = fmaf(D[50], m, L[16]);
-      L[17] = fmaf(D[51], m, L[17]);
-      L[18] = fmaf(D[52], m, L[18]);
-      L[19] = fmaf(D[53], m, L[19]);
-      L[20] = fmaf(D[59], m, L[20]);
-      L[21] = fmaf(D[62], m, L[21]);
-      L[22] = fmaf(D[63], m, L[22]);
-      L[23] = fmaf(D[66], m, L[23]);
-      L[24] = fmaf(D[67], m, L[24]);
-      L[25] = fmaf(D[68], m, L[25]);
-      L[26] = fmaf(D[71], m, L[26]);
-      L[27] = fmaf(D[72], m, L[27]);
-      L[28] = fmaf(D[73], m, L[28]);
-      L[29] = fmaf(D[74], m, L[29]);
-      L[30] = fmaf(D[77], m, L[30]);
-      L[31] = fmaf(D[78], m, L[31]);
-      L[32] = fmaf(D[79], m, L[32]);
-      L[33] = fmaf(D[80], m, L[33]);
-      L[34] = fmaf(D[81], m, L[34]);
-    }
-    { const float m = __ldg(Ms + 8) * rp;
-      L[0] = fmaf(D[8], m, L[0]);
-      L[1] = fmaf(D[14], m, L[1]);
-      L[2] = fmaf(D[17], m, L[2]);
-      L[3] = fmaf(D[18], m, L[3]);
-      L[4] = fmaf(D[24], m, L[4]);
-      L[5] = fmaf(D[27], m, L[5]);
-      L[6] = fmaf(D[28], m, L[6]);
-      L[7] = fmaf(D[31], m, L[7]);
-      L[8] = fmaf(D[32], m, L[8]);
-      L[9] = fmaf(D[33], m, L[9]);
-      L[10] = fmaf(D[39], m, L[10]);
-      L[11] = fmaf(D[42], m, L[11]);
-      L[12] = fmaf(D[43], m, L[12]);
-      L[13] = fmaf(D[46], m, L[13]);
-      L[14] = fmaf(D[47], m, L[14]);
-      L[15] = fmaf(D[48], m, L[15]);
-      L[16] = fmaf(D[51], m, L[16]);
-      L[17] = fmaf(D[52], m, L[17]);
-      L[18] = fmaf(D[53], m, L[18]);
-      L[19] = fmaf(D[54], m, L[19]);
-      L[20] = fmaf(D[60], m, L[20]);
-      L[21] = fmaf(D[63], m, L[21]);
-      L[22] = fmaf(D[64], m, L[22]);
-      L[23] = fmaf(D[67], m, L[23]);
-      L[24] = fmaf(D[68], m, L[24]);
-      L[25] = fmaf(D[69], m, L[25]);
-      L[26] = fmaf(D[72], m, L[26]);
-      L[27] = fmaf(D[73], m, L[27]);
-      L[28] = fmaf(D[74], m, L[28]);
-      L[29] = fmaf(D[75], m, L[29]);
-      L[30] = fmaf(D[78], m, L[30]);
-      L[31] = fmaf(D[79], m, L[31]);
-      L[32] = fmaf(D[80], m, L[32]);
-      L[33] = fmaf(D[81], m, L[33]);
-      L[34] = fmaf(D[82], m, L[34]);
-    }
-    { const float m = __ldg(Ms + 9) * rp;
-      L[0] = fmaf(D[9], m, L[0]);
-      L[1] = fmaf(D[15], m, L[1]);
-      L[2] = fmaf(D[18], m, L[2]);
-      L[3] = fmaf(D[19], m, L[3]);
-      L[4] = fmaf(D[25], m, L[4]);
-      L[5] = fmaf(D[28], m, L[5]);
-      L[6] = fmaf(D[29], m, L[6]);
-      L[7] = fmaf(D[32], m, L[7]);
-      L[8] = fmaf(D[33], m, L[8]);
-      L[9] = fmaf(D[34], m, L[9]);
-      L[10] = fmaf(D[40], m, L[10]);
-      L[11] = fmaf(D[43], m, L[11]);
-      L[12] = fmaf(D[44], m, L[12]);
-      L[13] = fmaf(D[47], m, L[13]);
-      L[14] = fmaf(D[48], m, L[14]);
-      L[15] = fmaf(D[49], m, L[15]);
-      L[16] = fmaf(D[52], m, L[16]);
-      L[17] = fmaf(D[53], m, L[17]);
-      L[18] = fmaf(D[54], m, L[18]);
-      L[19] = fmaf(D[55], m, L[19]);
-      L[20] = fmaf(D[61], m, L[20]);
-      L[21] = fmaf(D[64], m, L[21]);
-      L[22] = fmaf(D[65], m, L[22]);
-      L[23] = fmaf(D[68], m, L[23]);
-      L[24] = fmaf(D[69], m, L[24]);
-      L[25] = fmaf(D[70], m, L[25]);
-      L[26] = fmaf(D[73], m, L[26]);
-      L[27] = fmaf(D[74], m, L[27]);
-      L[28] = fmaf(D[75], m, L[28]);
-      L[29] = fmaf(D[76], m, L[29]);
-      L[30] = fmaf(D[79], m, L[30]);
-      L[31] = fmaf(D[80], m, L[31]);
-      L[32] = fmaf(D[81], m, L[32]);
-      L[33] = fmaf(D[82], m, L[33]);
-      L[34] = fmaf(D[83], m, L[34]);
+    { const T m = -__ldg(Ms + 3) * rp;
+      L[0] = m2l_fma(D[3], m, L[0]);
+      L[1] = m2l_fma(D[6], m, L[1]);
+      L[2] = m2l_fma(D[8], m, L[2]);
+      L[3] = m2l_fma(D[9], m, L[3]);
+      L[4] = m2l_fma(D[12], m, L[4]);
+      L[5] = m2l_fma(D[14], m, L[5]);
+      L[6] = m2l_fma(D[15], m, L[6]);
+      L[7] = m2l_fma(D[17], m, L[7]);
+      L[8] = m2l_fma(D[18], m, L[8]);
+      L[9] = m2l_fma(D[19], m, L[9]);
+      L[10] = m2l_fma(D[22], m, L[10]);
+      L[11] = m2l_fma(D[24], m, L[11]);
+      L[12] = m2l_fma(D[25], m, L[12]);
+      L[13] = m2l_fma(D[27], m, L[13]);
+      L[14] = m2l_fma(D[28], m, L[14]);
+      L[15] = m2l_fma(D[29], m, L[15]);
+      L[16] = m2l_fma(D[31], m, L[16]);
+      L[17] = m2l_fma(D[32], m, L[17]);
+      L[18] = m2l_fma(D[33], m, L[18]);
+      L[19] = m2l_fma(D[34], m, L[19]);
+      L[20] = m2l_fma(D[37], m, L[20]);
+      L[21] = m2l_fma(D[39], m, L[21]);
+      L[22] = m2l_fma(D[40], m, L[22]);
+      L[23] = m2l_fma(D[42], m, L[23]);
+      L[24] = m2l_fma(D[43], m, L[24]);
+      L[25] = m2l_fma(D[44], m, L[25]);
+      L[26] = m2l_fma(D[46], m, L[26]);
+      L[27] = m2l_fma(D[47], m, L[27]);
+      L[28] = m2l_fma(D[48], m, L[28]);
+      L[29] = m2l_fma(D[49], m, L[29]);
+      L[30] = m2l_fma(D[51], m, L[30]);
+      L[31] = m2l_fma(D[52], m, L[31]);
+      L[32] = m2l_fma(D[53], m, L[32]);
+      L[33] = m2l_fma(D[54], m, L[33]);
+      L[34] = m2l_fma(D[55], m, L[34]);
+      L[35] = m2l_fma(D[58], m, L[35]);
+      L[36] = m2l_fma(D[60], m, L[36]);
+      L[37] = m2l_fma(D[61], m, L[37]);
+      L[38] = m2l_fma(D[63], m, L[38]);
+      L[39] = m2l_fma(D[64], m, L[39]);
+      L[40] = m2l_fma(D[65], m, L[40]);
+      L[41] = m2l_fma(D[67], m, L[41]);
+      L[42] = m2l_fma(D[68], m, L[42]);
+      L[43] = m2l_fma(D[69], m, L[43]);
+      L[44] = m2l_fma(D[70], m, L[44]);
+      L[45] = m2l_fma(D[72], m, L[45]);
+      L[46] = m2l_fma(D[73], m, L[46]);
+      L[47] = m2l_fma(D[74], m, L[47]);
+      L[48] = m2l_fma(D[75], m, L[48]);
+      L[49] = m2l_fma(D[76], m, L[49]);
+      L[50] = m2l_fma(D[78], m, L[50]);
+      L[51] = m2l_fma(D[79], m, L[51]);
+      L[52] = m2l_fma(D[80], m, L[52]);
+      L[53] = m2l_fma(D[81], m, L[53]);
+      L[54] = m2l_fma(D[82], m, L[54]);
+      L[55] = m2l_fma(D[83], m, L[55]);
     }
     rp *= rho;
-    { const float m = -__ldg(Ms + 10) * rp;
-      L[0] = fmaf(D[10], m, L[0]);
-      L[1] = fmaf(D[20], m, L[1]);
-      L[2] = fmaf(D[21], m, L[2]);
-      L[3] = fmaf(D[22], m, L[3]);
-      L[4] = fmaf(D[35], m, L[4]);
-      L[5] = fmaf(D[36], m, L[5]);
-      L[6] = fmaf(D[37], m, L[6]);
-      L[7] = fmaf(D[38], m, L[7]);
-      L[8] = fmaf(D[39], m, L[8]);
-      L[9] = fmaf(D[40], m, L[9]);
-      L[10] = fmaf(D[56], m, L[10]);
-      L[11] = fmaf(D[57], m, L[11]);
-      L[12] = fmaf(D[58], m, L[12]);
-      L[13] = fmaf(D[59], m, L[13]);
-      L[14] = fmaf(D[60], m, L[14]);
-      L[15] = fmaf(D[61], m, L[15]);
-      L[16] = fmaf(D[62], m, L[16]);
-      L[17] = fmaf(D[63], m, L[17]);
-      L[18] = fmaf(D[64], m, L[18]);
-      L[19] = fmaf(D[65], m, L[19]);
+    { const T m = __ldg(Ms + 4) * rp;
+      L[0] = m2l_fma(D[4], m, L[0]);
+      L[1] = m2l_fma(D[10], m, L[1]);
+      L[2] = m2l_fma(D[11], m, L[2]);
+      L[3] = m2l_fma(D[12], m, L[3]);
+      L[4] = m2l_fma(D[20], m, L[4]);
+      L[5] = m2l_fma(D[21], m, L[5]);
+      L[6] = m2l_fma(D[22], m, L[6]);
+      L[7] = m2l_fma(D[23], m, L[7]);
+      L[8] = m2l_fma(D[24], m, L[8]);
+      L[9] = m2l_fma(D[25], m, L[9]);
+      L[10] = m2l_fma(D[35], m, L[10]);
+      L[11] = m2l_fma(D[36], m, L[11]);
+      L[12] = m2l_fma(D[37], m, L[12]);
+      L[13] = m2l_fma(D[38], m, L[13]);
+      L[14] = m2l_fma(D[39], m, L[14]);
+      L[15] = m2l_fma(D[40], m, L[15]);
+      L[16] = m2l_fma(D[41], m, L[16]);
+      L[17] = m2l_fma(D[42], m, L[17]);
+      L[18] = m2l_fma(D[43], m, L[18]);
+      L[19] = m2l_fma(D[44], m, L[19]);
+      L[20] = m2l_fma(D[56], m, L[20]);
+      L[21] = m2l_fma(D[57], m, L[21]);
+      L[22] = m2l_fma(D[58], m, L[22]);
+      L[23] = m2l_fma(D[59], m, L[23]);
+      L[24] = m2l_fma(D[60], m, L[24]);
+      L[25] = m2l_fma(D[61], m, L[25]);
+      L[26] = m2l_fma(D[62], m, L[26]);
+      L[27] = m2l_fma(D[63], m, L[27]);
+      L[28] = m2l_fma(D[64], m, L[28]);
+      L[29] = m2l_fma(D[65], m, L[29]);
+      L[30] = m2l_fma(D[66], m, L[30]);
+      L[31] = m2l_fma(D[67], m, L[31]);
+      L[32] = m2l_fma(D[68], m, L[32]);
+      L[33] = m2l_fma(D[69], m, L[33]);
+      L[34] = m2l_fma(D[70], m, L[34]);
     }
-    { const float m = -__ldg(Ms + 11) * rp;
-      L[0] = fmaf(D[11], m, L[0]);
-      L[1] = fmaf(D[21], m, L[1]);
-      L[2] = fmaf(D[23], m, L[2]);
-      L[3] = fmaf(D[24], m, L[3]);
-      L[4] = fmaf(D[36], m, L[4]);
-      L[5] = fmaf(D[38], m, L[5]);
-      L[6] = fmaf(D[39], m, L[6]);
-      L[7] = fmaf(D[41], m, L[7]);
-      L[8] = fmaf(D[42], m, L[8]);
-      L[9] = fmaf(D[43], m, L[9]);
-      L[10] = fmaf(D[57], m, L[10]);
-      L[11] = fmaf(D[59], m, L[11]);
-      L[12] = fmaf(D[60], m, L[12]);
-      L[13] = fmaf(D[62], m, L[13]);
-      L[14] = fmaf(D[63], m, L[14]);
-      L[15] = fmaf(D[64], m, L[15]);
-      L[16] = fmaf(D[66], m, L[16]);
-      L[17] = fmaf(D[67], m, L[17]);
-      L[18] = fmaf(D[68], m, L[18]);
-      L[19] = fmaf(D[69], m, L[19]);
+    { const T m = __ldg(Ms + 5) * rp;
+      L[0] = m2l_fma(D[5], m, L[0]);
+      L[1] = m2l_fma(D[11], m, L[1]);
+      L[2] = m2l_fma(D[13], m, L[2]);
+      L[3] = m2l_fma(D[14], m, L[3]);
+      L[4] = m2l_fma(D[21], m, L[4]);
+      L[5] = m2l_fma(D[23], m, L[5]);
+      L[6] = m2l_fma(D[24], m, L[6]);
+      L[7] = m2l_fma(D[26], m, L[7]);
+      L[8] = m2l_fma(D[27], m, L[8]);
+      L[9] = m2l_fma(D[28], m, L[9]);
+      L[10] = m2l_fma(D[36], m, L[10]);
+      L[11] = m2l_fma(D[38], m, L[11]);
+      L[12] = m2l_fma(D[39], m, L[12]);
+      L[13] = m2l_fma(D[41], m, L[13]);
+      L[14] = m2l_fma(D[42], m, L[14]);
+      L[15] = m2l_fma(D[43], m, L[15]);
+      L[16] = m2l_fma(D[45], m, L[16]);
+      L[17] = m2l_fma(D[46], m, L[17]);
+      L[18] = m2l_fma(D[47], m, L[18]);
+      L[19] = m2l_fma(D[48], m, L[19]);
+      L[20] = m2l_fma(D[57], m, L[20]);
+      L[21] = m2l_fma(D[59], m, L[21]);
+      L[22] = m2l_fma(D[60], m, L[22]);
+      L[23] = m2l_fma(D[62], m, L[23]);
+      L[24] = m2l_fma(D[63], m, L[24]);
+      L[25] = m2l_fma(D[64], m, L[25]);
+      L[26] = m2l_fma(D[66], m, L[26]);
+      L[27] = m2l_fma(D[67], m, L[27]);
+      L[28] = m2l_fma(D[68], m, L[28]);
+      L[29] = m2l_fma(D[69], m, L[29]);
+      L[30] = m2l_fma(D[71], m, L[30]);
+      L[31] = m2l_fma(D[72], m, L[31]);
+      L[32] = m2l_fma(D[73], m, L[32]);
+      L[33] = m2l_fma(D[74], m, L[33]);
+      L[34] = m2l_fma(D[75], m, L[34]);
     }
-    { const float m = -__ldg(Ms + 12) * rp;
-      L[0] = fmaf(D[12], m, L[0]);
-      L[1] = fmaf(D[22], m, L[1]);
-      L[2] = fmaf(D[24], m, L[2]);
-      L[3] = fmaf(D[25], m, L[3]);
-      L[4] = fmaf(D[37], m, L[4]);
-      L[5] = fmaf(D[39], m, L[5]);
-      L[6] = fmaf(D[40], m, L[6]);
-      L[7] = fmaf(D[42], m, L[7]);
-      L[8] = fmaf(D[43], m, L[8]);
-      L[9] = fmaf(D[44], m, L[9]);
-      L[10] = fmaf(D[58], m, L[10]);
-      L[11] = fmaf(D[60], m, L[11]);
-      L[12] = fmaf(D[61], m, L[12]);
-      L[13] = fmaf(D[63], m, L[13]);
-      L[14] = fmaf(D[64], m, L[14]);
-      L[15] = fmaf(D[65], m, L[15]);
-      L[16] = fmaf(D[67], m, L[16]);
-      L[17] = fmaf(D[68], m, L[17]);
-      L[18] = fmaf(D[69], m, L[18]);
-      L[19] = fmaf(D[70], m, L[19]);
+    { const T m = __ldg(Ms + 6) * rp;
+      L[0] = m2l_fma(D[6], m, L[0]);
+      L[1] = m2l_fma(D[12], m, L[1]);
+      L[2] = m2l_fma(D[14], m, L[2]);
+      L[3] = m2l_fma(D[15], m, L[3]);
+      L[4] = m2l_fma(D[22], m, L[4]);
+      L[5] = m2l_fma(D[24], m, L[5]);
+      L[6] = m2l_fma(D[25], m, L[6]);
+      L[7] = m2l_fma(D[27], m, L[7]);
+      L[8] = m2l_fma(D[28], m, L[8]);
+      L[9] = m2l_fma(D[29], m, L[9]);
+      L[10] = m2l_fma(D[37], m, L[10]);
+      L[11] = m2l_fma(D[39], m, L[11]);
+      L[12] = m2l_fma(D[40], m, L[12]);
+      L[13] = m2l_fma(D[42], m, L[13]);
+      L[14] = m2l_fma(D[43], m, L[14]);
+      L[15] = m2l_fma(D[44], m, L[15]);
+      L[16] = m2l_fma(D[46], m, L[16]);
+      L[17] = m2l_fma(D[47], m, L[17]);
+      L[18] = m2l_fma(D[48], m, L[18]);
+      L[19] = m2l_fma(D[49], m, L[19]);
+      L[20] = m2l_fma(D[58], m, L[20]);
+      L[21] = m2l_fma(D[60], m, L[21]);
+      L[22] = m2l_fma(D[61], m, L[22]);
+      L[23] = m2l_fma(D[63], m, L[23]);
+      L[24] = m2l_fma(D[64], m, L[24]);
+      L[25] = m2l_fma(D[65], m, L[25]);
+      L[26] = m2l_fma(D[67], m, L[26]);
+      L[27] = m2l_fma(D[68], m, L[27]);
+      L[28] = m2l_fma(D[69], m, L[28]);
+      L[29] = m2l_fma(D[70], m, L[29]);
+      L[30] = m2l_fma(D[72], m, L[30]);
+      L[31] = m2l_fma(D[73], m, L[31]);
+      L[32] = m2l_fma(D[74], m, L[32]);
+      L[33] = m2l_fma(D[75], m, L[33]);
+      L[34] = m2l_fma(D[76], m, L[34]);
     }
-    { const float m = -__ldg(Ms + 13) * rp;
-      L[0] = fmaf(D[13], m, L[0]);
-      L[1] = fmaf(D[23], m, L[1]);
-      L[2] = fmaf(D[26], m, L[2]);
-      L[3] = fmaf(D[27], m, L[3]);
-      L[4] = fmaf(D[38], m, L[4]);
-      L[5] = fmaf(D[41], m, L[5]);
-      L[6] = fmaf(D[42], m, L[6]);
-      L[7] = fmaf(D[45], m, L[7]);
-      L[8] = fmaf(D[46], m, L[8]);
-      L[9] = fmaf(D[47], m, L[9]);
-      L[10] = fmaf(D[59], m, L[10]);
-      L[11] = fmaf(D[62], m, L[11]);
-      L[12] = fmaf(D[63], m, L[12]);
-      L[13] = fmaf(D[66], m, L[13]);
-      L[14] = fmaf(D[67], m, L[14]);
-      L[15] = fmaf(D[68], m, L[15]);
-      L[16] = fmaf(D[71], m, L[16]);
-      L[17] = fmaf(D[72], m, L[17]);
-      L[18] = fmaf(D[73], m, L[18]);
-      L[19] = fmaf(D[74], m, L[19]);
+    { const T m = __ldg(Ms + 7) * rp;
+      L[0] = m2l_fma(D[7], m, L[0]);
+      L[1] = m2l_fma(D[13], m, L[1]);
+      L[2] = m2l_fma(D[16], m, L[2]);
+      L[3] = m2l_fma(D[17], m, L[3]);
+      L[4] = m2l_fma(D[23], m, L[4]);
+      L[5] = m2l_fma(D[26], m, L[5]);
+      L[6] = m2l_fma(D[27], m, L[6]);
+      L[7] = m2l_fma(D[30], m, L[7]);
+      L[8] = m2l_fma(D[31], m, L[8]);
+      L[9] = m2l_fma(D[32], m, L[9]);
+      L[10] = m2l_fma(D[38], m, L[10]);
+      L[11] = m2l_fma(D[41], m, L[11]);
+      L[12] = m2l_fma(D[42], m, L[12]);
+      L[13] = m2l_fma(D[45], m, L[13]);
+      L[14] = m2l_fma(D[46], m, L[14]);
+      L[15] = m2l_fma(D[47], m, L[15]);
+      L[16] = m2l_fma(D[50], m, L[16]);
+      L[17] = m2l_fma(D[51], m, L[17]);
+      L[18] = m2l_fma(D[52], m, L[18]);
+      L[19] = m2l_fma(D[53], m, L[19]);
+      L[20] = m2l_fma(D[59], m, L[20]);
+      L[21] = m2l_fma(D[62], m, L[21]);
+      L[22] = m2l_fma(D[63], m, L[22]);
+      L[23] = m2l_fma(D[66], m, L[23]);
+      L[24] = m2l_fma(D[67], m, L[24]);
+      L[25] = m2l_fma(D[68], m, L[25]);
+      L[26] = m2l_fma(D[71], m, L[26]);
+      L[27] = m2l_fma(D[72], m, L[27]);
+      L[28] = m2l_fma(D[73], m, L[28]);
+      L[29] = m2l_fma(D[74], m, L[29]);
+      L[30] = m2l_fma(D[77], m, L[30]);
+      L[31] = m2l_fma(D[78], m, L[31]);
+      L[32] = m2l_fma(D[79], m, L[32]);
+      L[33] = m2l_fma(D[80], m, L[33]);
+      L[34] = m2l_fma(D[81], m, L[34]);
     }
-    { const float m = -__ldg(Ms + 14) * rp;
-      L[0] = fmaf(D[14], m, L[0]);
-      L[1] = fmaf(D[24], m, L[1]);
-      L[2] = fmaf(D[27], m, L[2]);
-      L[3] = fmaf(D[28], m, L[3]);
-      L[4] = fmaf(D[39], m, L[4]);
-      L[5] = fmaf(D[42], m, L[5]);
-      L[6] = fmaf(D[43], m, L[6]);
-      L[7] = fmaf(D[46], m, L[7]);
-      L[8] = fmaf(D[47], m, L[8]);
-      L[9] = fmaf(D[48], m, L[9]);
-      L[10] = fmaf(D[60], m, L[10]);
-      L[11] = fmaf(D[63], m, L[11]);
-      L[12] = fmaf(D[64], m, L[12]);
-      L[13] = fmaf(D[67], m, L[13]);
-      L[14] = fmaf(D[68], m, L[14]);
-      L[15] = fmaf(D[69], m, L[15]);
-      L[16] = fmaf(D[72], m, L[16]);
-      L[17] = fmaf(D[73], m, L[17]);
-      L[18] = fmaf(D[74], m, L[18]);
-      L[19] = fmaf(D[75], m, L[19]);
+    { const T m = __ldg(Ms + 8) * rp;
+      L[0] = m2l_fma(D[8], m, L[0]);
+      L[1] = m2l_fma(D[14], m, L[1]);
+      L[2] = m2l_fma(D[17], m, L[2]);
+      L[3] = m2l_fma(D[18], m, L[3]);
+      L[4] = m2l_fma(D[24], m, L[4]);
+      L[5] = m2l_fma(D[27], m, L[5]);
+      L[6] = m2l_fma(D[28], m, L[6]);
+      L[7] = m2l_fma(D[31], m, L[7]);
+      L[8] = m2l_fma(D[32], m, L[8]);
+      L[9] = m2l_fma(D[33], m, L[9]);
+      L[10] = m2l_fma(D[39], m, L[10]);
+      L[11] = m2l_fma(D[42], m, L[11]);
+      L[12] = m2l_fma(D[43], m, L[12]);
+      L[13] = m2l_fma(D[46], m, L[13]);
+      L[14] = m2l_fma(D[47], m, L[14]);
+      L[15] = m2l_fma(D[48], m, L[15]);
+      L[16] = m2l_fma(D[51], m, L[16]);
+      L[17] = m2l_fma(D[52], m, L[17]);
+      L[18] = m2l_fma(D[53], m, L[18]);
+      L[19] = m2l_fma(D[54], m, L[19]);
+      L[20] = m2l_fma(D[60], m, L[20]);
+      L[21] = m2l_fma(D[63], m, L[21]);
+      L[22] = m2l_fma(D[64], m, L[22]);
+      L[23] = m2l_fma(D[67], m, L[23]);
+      L[24] = m2l_fma(D[68], m, L[24]);
+      L[25] = m2l_fma(D[69], m, L[25]);
+      L[26] = m2l_fma(D[72], m, L[26]);
+      L[27] = m2l_fma(D[73], m, L[27]);
+      L[28] = m2l_fma(D[74], m, L[28]);
+      L[29] = m2l_fma(D[75], m, L[29]);
+      L[30] = m2l_fma(D[78], m, L[30]);
+      L[31] = m2l_fma(D[79], m, L[31]);
+      L[32] = m2l_fma(D[80], m, L[32]);
+      L[33] = m2l_fma(D[81], m, L[33]);
+      L[34] = m2l_fma(D[82], m, L[34]);
     }
-    { const float m = -__ldg(Ms + 15) * rp;
-      L[0] = fmaf(D[15], m, L[0]);
-      L[1] = fmaf(D[25], m, L[1]);
-      L[2] = fmaf(D[28], m, L[2]);
-      L[3] = fmaf(D[29], m, L[3]);
-      L[4] = fmaf(D[40], m, L[4]);
-      L[5] = fmaf(D[43], m, L[5]);
-      L[6] = fmaf(D[44], m, L[6]);
-      L[7] = fmaf(D[47], m, L[7]);
-      L[8] = fmaf(D[48], m, L[8]);
-      L[9] = fmaf(D[49], m, L[9]);
-      L[10] = fmaf(D[61], m, L[10]);
-      L[11] = fmaf(D[64], m, L[11]);
-      L[12] = fmaf(D[65], m, L[12]);
-      L[13] = fmaf(D[68], m, L[13]);
-      L[14] = fmaf(D[69], m, L[14]);
-      L[15] = fmaf(D[70], m, L[15]);
-      L[16] = fmaf(D[73], m, L[16]);
-      L[17] = fmaf(D[74], m, L[17]);
-      L[18] = fmaf(D[75], m, L[18]);
-      L[19] = fmaf(D[76], m, L[19]);
-    }
-    { const float m = -__ldg(Ms + 16) * rp;
-      L[0] = fmaf(D[16], m, L[0]);
-      L[1] = fmaf(D[26], m, L[1]);
-      L[2] = fmaf(D[30], m, L[2]);
-      L[3] = fmaf(D[31], m, L[3]);
-      L[4] = fmaf(D[41], m, L[4]);
-      L[5] = fmaf(D[45], m, L[5]);
-      L[6] = fmaf(D[46], m, L[6]);
-      L[7] = fmaf(D[50], m, L[7]);
-      L[8] = fmaf(D[51], m, L[8]);
-      L[9] = fmaf(D[52], m, L[9]);
-      L[10] = fmaf(D[62], m, L[10]);
-      L[11] = fmaf(D[66], m, L[11]);
-      L[12] = fmaf(D[67], m, L[12]);
-      L[13] = fmaf(D[71], m, L[13]);
-      L[14] = fmaf(D[72], m, L[14]);
-      L[15] = fmaf(D[73], m, L[15]);
-      L[16] = fmaf(D[77], m, L[16]);
-      L[17] = fmaf(D[78], m, L[17]);
-      L[18] = fmaf(D[79], m, L[18]);
-      L[19] = fmaf(D[80], m, L[19]);
-    }
-    { const float m = -__ldg(Ms + 17) * rp;
-      L[0] = fmaf(D[17], m, L[0]);
-      L[1] = fmaf(D[27], m, L[1]);
-      L[2] = fmaf(D[31], m, L[2]);
-      L[3] = fmaf(D[32], m, L[3]);
-      L[4] = fmaf(D[42], m, L[4]);
-      L[5] = fmaf(D[46], m, L[5]);
-      L[6] = fmaf(D[47], m, L[6]);
-      L[7] = fmaf(D[51], m, L[7]);
-      L[8] = fmaf(D[52], m, L[8]);
-      L[9] = fmaf(D[53], m, L[9]);
-      L[10] = fmaf(D[63], m, L[10]);
-      L[11] = fmaf(D[67], m, L[11]);
-      L[12] = fmaf(D[68], m, L[12]);
-      L[13] = fmaf(D[72], m, L[13]);
-      L[14] = fmaf(D[73], m, L[14]);
-      L[15] = fmaf(D[74], m, L[15]);
-      L[16] = fmaf(D[78], m, L[16]);
-      L[17] = fmaf(D[79], m, L[17]);
-      L[18] = fmaf(D[80], m, L[18]);
-      L[19] = fmaf(D[81], m, L[19]);
-    }
-    { const float m = -__ldg(Ms + 18) * rp;
-      L[0] = fmaf(D[18], m, L[0]);
-      L[1] = fmaf(D[28], m, L[1]);
-      L[2] = fmaf(D[32], m, L[2]);
-      L[3] = fmaf(D[33], m, L[3]);
-      L[4] = fmaf(D[43], m, L[4]);
-      L[5] = fmaf(D[47], m, L[5]);
-      L[6] = fmaf(D[48], m, L[6]);
-      L[7] = fmaf(D[52], m, L[7]);
-      L[8] = fmaf(D[53], m, L[8]);
-      L[9] = fmaf(D[54], m, L[9]);
-      L[10] = fmaf(D[64], m, L[10]);
-      L[11] = fmaf(D[68], m, L[11]);
-      L[12] = fmaf(D[69], m, L[12]);
-      L[13] = fmaf(D[73], m, L[13]);
-      L[14] = fmaf(D[74], m, L[14]);
-      L[15] = fmaf(D[75], m, L[15]);
-      L[16] = fmaf(D[79], m, L[16]);
-      L[17] = fmaf(D[80], m, L[17]);
-      L[18] = fmaf(D[81], m, L[18]);
-      L[19] = fmaf(D[82], m, L[19]);
-    }
-    { const float m = -__ldg(Ms + 19) * rp;
-      L[0] = fmaf(D[19], m, L[0]);
-      L[1] = fmaf(D[29], m, L[1]);
-      L[2] = fmaf(D[33], m, L[2]);
-      L[3] = fmaf(D[34], m, L[3]);
-      L[4] = fmaf(D[44], m, L[4]);
-      L[5] = fmaf(D[48], m, L[5]);
-      L[6] = fmaf(D[49], m, L[6]);
-      L[7] = fmaf(D[53], m, L[7]);
-      L[8] = fmaf(D[54], m, L[8]);
-      L[9] = fmaf(D[55], m, L[9]);
-      L[10] = fmaf(D[65], m, L[10]);
-      L[11] = fmaf(D[69], m, L[11]);
-      L[12] = fmaf(D[70], m, L[12]);
-      L[13] = fmaf(D[74], m, L[13]);
-      L[14] = fmaf(D[75], m, L[14]);
-      L[15] = fmaf(D[76], m, L[15]);
-      L[16] = fmaf(D[80], m, L[16]);
-      L[17] = fmaf(D[81], m, L[17]);
-      L[18] = fmaf(D[82], m, L[18]);
-      L[19] = fmaf(D[83], m, L[19]);
-    }
-    rp *= rho;
-    { const float m = __ldg(Ms + 20) * rp;
-      L[0] = fmaf(D[20], m, L[0]);
-      L[1] = fmaf(D[35], m, L[1]);
-      L[2] = fmaf(D[36], m, L[2]);
-      L[3] = fmaf(D[37], m, L[3]);
-      L[4] = fmaf(D[56], m, L[4]);
-      L[5] = fmaf(D[57], m, L[5]);
-      L[6] = fmaf(D[58], m, L[6]);
-      L[7] = fmaf(D[59], m, L[7]);
-      L[8] = fmaf(D[60], m, L[8]);
-      L[9] = fmaf(D[61], m, L[9]);
-    }
-    { const float m = __ldg(Ms + 21) * rp;
-      L[0] = fmaf(D[21], m, L[0]);
-      L[1] = fmaf(D[36], m, L[1]);
-      L[2] = fmaf(D[38], m, L[2]);
-      L[3] = fmaf(D[39], m, L[3]);
-      L[4] = fmaf(D[57], m, L[4]);
-      L[5] = fmaf(D[59], m, L[5]);
-      L[6] = fmaf(D[60], m, L[6]);
-      L[7] = fmaf(D[62], m, L[7]);
-      L[8] = fmaf(D[63], m, L[8]);
-      L[9] = fmaf(D[64], m, L[9]);
-    }
-    { const float m = __ldg(Ms + 22) * rp;
-      L[0] = fmaf(D[22], m, L[0]);
-      L[1] = fmaf(D[37], m, L[1]);
-      L[2] = fmaf(D[39], m, L[2]);
-      L[3] = fmaf(D[40], m, L[3]);
-      L[4] = fmaf(D[58], m, L[4]);
-      L[5] = fmaf(D[60], m, L[5]);
-      L[6] = fmaf(D[61], m, L[6]);
-      L[7] = fmaf(D[63], m, L[7]);
-      L[8] = fmaf(D[64], m, L[8]);
-      L[9] = fmaf(D[65], m, L[9]);
-    }
-    { const float m = __ldg(Ms + 23) * rp;
-      L[0] = fmaf(D[23], m, L[0]);
-      L[1] = fmaf(D[38], m, L[1]);
-      L[2] = fmaf(D[41], m, L[2]);
-      L[3] = fmaf(D[42], m, L[3]);
-      L[4] = fmaf(D[59], m, L[4]);
-      L[5] = fmaf(D[62], m, L[5]);
-      L[6] = fmaf(D[63], m, L[6]);
-      L[7] = fmaf(D[66], m, L[7]);
-      L[8] = fmaf(D[67], m, L[8]);
-      L[9] = fmaf(D[68], m, L[9]);
-    }
-    { const float m = __ldg(Ms + 24) * rp;
-      L[0] = fmaf(D[24], m, L[0]);
-      L[1] = fmaf(D[39], m, L[1]);
-      L[2] = fmaf(D[42], m, L[2]);
-      L[3] = fmaf(D[43], m, L[3]);
-      L[4] = fmaf(D[60], m, L[4]);
-      L[5] = fmaf(D[63], m, L[5]);
-      L[6] = fmaf(D[64], m, L[6]);
-      L[7] = fmaf(D[67], m, L[7]);
-      L[8] = fmaf(D[68], m, L[8]);
-      L[9] = fmaf(D[69], m, L[9]);
-    }
-    { const float m = __ldg(Ms + 25) * rp;
-      L[0] = fmaf(D[25], m, L[0]);
-      L[1] = fmaf(D[40], m, L[1]);
-      L[2] = fmaf(D[43], m, L[2]);
-      L[3] = fmaf(D[44], m, L[3]);
-      L[4] = fmaf(D[61], m, L[4]);
-      L[5] = fmaf(D[64], m, L[5]);
-      L[6] = fmaf(D[65], m, L[6]);
-      L[7] = fmaf(D[68], m, L[7]);
-      L[8] = fmaf(D[69], m, L[8]);
-      L[9] = fmaf(D[70], m, L[9]);
-    }
-    { const float m = __ldg(Ms + 26) * rp;
-      L[0] = fmaf(D[26], m, L[0]);
-      L[1] = fmaf(D[41], m, L[1]);
-      L[2] = fmaf(D[45], m, L[2]);
-      L[3] = fmaf(D[46], m, L[3]);
-      L[4] = fmaf(D[62], m, L[4]);
-      L[5] = fmaf(D[66], m, L[5]);
-      L[6] = fmaf(D[67], m, L[6]);
-      L[7] = fmaf(D[71], m, L[7]);
-      L[8] = fmaf(D[72], m, L[8]);
-      L[9] = fmaf(D[73], m, L[9]);
-    }
-    { const float m = __ldg(Ms + 27) * rp;
-      L[0] = fmaf(D[27], m, L[0]);
-      L[1] = fmaf(D[42], m, L[1]);
-      L[2] = fmaf(D[46], m, L[2]);
-      L[3] = fmaf(D[47], m, L[3]);
-      L[4] = fmaf(D[63], m, L[4]);
-      L[5] = fmaf(D[67], m, L[5]);
-      L[6] = fmaf(D[68], m, L[6]);
-      L[7] = fmaf(D[72], m, L[7]);
-      L[8] = fmaf(D[73], m, L[8]);
-      L[9] = fmaf(D[74], m, L[9]);
-    }
-    { const float m = __ldg(Ms + 28) * rp;
-      L[0] = fmaf(D[28], m, L[0]);
-      L[1] = fmaf(D[43], m, L[1]);
-      L[2] = fmaf(D[47], m, L[2]);
-      L[3] = fmaf(D[48], m, L[3]);
-      L[4] = fmaf(D[64], m, L[4]);
-      L[5] = fmaf(D[68], m, L[5]);
-      L[6] = fmaf(D[69], m, L[6]);
-      L[7] = fmaf(D[73], m, L[7]);
-      L[8] = fmaf(D[74], m, L[8]);
-      L[9] = fmaf(D[75], m, L[9]);
-    }
-    { const float m = __ldg(Ms + 29) * rp;
-      L[0] = fmaf(D[29], m, L[0]);
-      L[1] = fmaf(D[44], m, L[1]);
-      L[2] = fmaf(D[48], m, L[2]);
-      L[3] = fmaf(D[49], m, L[3]);
-      L[4] = fmaf(D[65], m, L[4]);
-      L[5] = fmaf(D[69], m, L[5]);
-      L[6] = fmaf(D[70], m, L[6]);
-      L[7] = fmaf(D[74], m, L[7]);
-      L[8] = fmaf(D[75], m, L[8]);
-      L[9] = fmaf(D[76], m, L[9]);
-    }
-    { const float m = __ldg(Ms + 30) * rp;
-      L[0] = fmaf(D[30], m, L[0]);
-      L[1] = fmaf(D[45], m, L[1]);
-      L[2] = fmaf(D[50], m, L[2]);
-      L[3] = fmaf(D[51], m, L[3]);
-      L[4] = fmaf(D[66], m, L[4]);
-      L[5] = fmaf(D[71], m, L[5]);
-      L[6] = fmaf(D[72], m, L[6]);
-      L[7] = fmaf(D[77], m, L[7]);
-      L[8] = fmaf(D[78], m, L[8]);
-      L[9] = fmaf(D[79], m, L[9]);
-    }
-    { const float m = __ldg(Ms + 31) * rp;
-      L[0] = fmaf(D[31], m, L[0]);
-      L[1] = fmaf(D[46], m, L[1]);
-      L[2] = fmaf(D[51], m, L[2]);
-      L[3] = fmaf(D[52], m, L[3]);
-      L[4] = fmaf(D[67], m, L[4]);
-      L[5] = fmaf(D[72], m, L[5]);
-      L[6] = fmaf(D[73], m, L[6]);
-      L[7] = fmaf(D[78], m, L[7]);
-      L[8] = fmaf(D[79], m, L[8]);
-      L[9] = fmaf(D[80], m, L[9]);
-    }
-    { const float m = __ldg(Ms + 32) * rp;
-      L[0] = fmaf(D[32], m, L[0]);
-      L[1] = fmaf(D[47], m, L[1]);
-      L[2] = fmaf(D[52], m, L[2]);
-      L[3] = fmaf(D[53], m, L[3]);
-      L[4] = fmaf(D[68], m, L[4]);
-      L[5] = fmaf(D[73], m, L[5]);
-      L[6] = fmaf(D[74], m, L[6]);
-      L[7] = fmaf(D[79], m, L[7]);
-      L[8] = fmaf(D[80], m, L[8]);
-      L[9] = fmaf(D[81], m, L[9]);
-    }
-    { const float m = __ldg(Ms + 33) * rp;
-      L[0] = fmaf(D[33], m, L[0]);
-      L[1] = fmaf(D[48], m, L[1]);
-      L[2] = fmaf(D[53], m, L[2]);
-      L[3] = fmaf(D[54], m, L[3]);
-      L[4] = fmaf(D[69], m, L[4]);
-      L[5] = fmaf(D[74], m, L[5]);
-      L[6] = fmaf(D[75], m, L[6]);
-      L[7] = fmaf(D[80], m, L[7]);
-      L[8] = fmaf(D[81], m, L[8]);
-      L[9] = fmaf(D[82], m, L[9]);
-    }
-    { const float m = __ldg(Ms + 34) * rp;
-      L[0] = fmaf(D[34], m, L[0]);
-      L[1] = fmaf(D[49], m, L[1]);
-      L[2] = fmaf(D[54], m, L[2]);
-      L[3] = fmaf(D[55], m, L[3]);
-      L[4] = fmaf(D[70], m, L[4]);
-      L[5] = fmaf(D[75], m, L[5]);
-      L[6] = fmaf(D[76], m, L[6]);
-      L[7] = fmaf(D[81], m, L[7]);
-      L[8] = fmaf(D[82], m, L[8]);
-      L[9] = fmaf(D[83], m, L[9]);
+    { const T m = __ldg(Ms + 9) * rp;
+      L[0] = m2l_fma(D[9], m, L[0]);
+      L[1] = m2l_fma(D[15], m, L[1]);
+      L[2] = m2l_fma(D[18], m, L[2]);
+      L[3] = m2l_fma(D[19], m, L[3]);
+      L[4] = m2l_fma(D[25], m, L[4]);
+      L[5] = m2l_fma(D[28], m, L[5]);
+      L[6] = m2l_fma(D[29], m, L[6]);
+      L[7] = m2l_fma(D[32], m, L[7]);
+      L[8] = m2l_fma(D[33], m, L[8]);
+      L[9] = m2l_fma(D[34], m, L[9]);
+      L[10] = m2l_fma(D[40], m, L[10]);
+      L[11] = m2l_fma(D[43], m, L[11]);
+      L[12] = m2l_fma(D[44], m, L[12]);
+      L[13] = m2l_fma(D[47], m, L[13]);
+      L[14] = m2l_fma(D[48], m, L[14]);
+      L[15] = m2l_fma(D[49], m, L[15]);
+      L[16] = m2l_fma(D[52], m, L[16]);
+      L[17] = m2l_fma(D[53], m, L[17]);
+      L[18] = m2l_fma(D[54], m, L[18]);
+      L[19] = m2l_fma(D[55], m, L[19]);
+      L[20] = m2l_fma(D[61], m, L[20]);
+      L[21] = m2l_fma(D[64], m, L[21]);
+      L[22] = m2l_fma(D[65], m, L[22]);
+      L[23] = m2l_fma(D[68], m, L[23]);
+      L[24] = m2l_fma(D[69], m, L[24]);
+      L[25] = m2l_fma(D[70], m, L[25]);
+      L[26] = m2l_fma(D[73], m, L[26]);
+      L[27] = m2l_fma(D[74], m, L[27]);
+      L[28] = m2l_fma(D[75], m, L[28]);
+      L[29] = m2l_fma(D[76], m, L[29]);
+      L[30] = m2l_fma(D[79], m, L[30]);
+      L[31] = m2l_fma(D[80], m, L[31]);
+      L[32] = m2l_fma(D[81], m, L[32]);
+      L[33] = m2l_fma(D[82], m, L[33]);
+      L[34] = m2l_fma(D[83], m, L[34]);
     }
     rp *= rho;
-    { const float m = -__ldg(Ms + 35) * rp;
-      L[0] = fmaf(D[35], m, L[0]);
-      L[1] = fmaf(D[56], m, L[1]);
-      L[2] = fmaf(D[57], m, L[2]);
-      L[3] = fmaf(D[58], m, L[3]);
+    { const T m = -__ldg(Ms + 10) * rp;
+      L[0] = m2l_fma(D[10], m, L[0]);
+      L[1] = m2l_fma(D[20], m, L[1]);
+      L[2] = m2l_fma(D[21], m, L[2]);
+      L[3] = m2l_fma(D[22], m, L[3]);
+      L[4] = m2l_fma(D[35], m, L[4]);
+      L[5] = m2l_fma(D[36], m, L[5]);
+      L[6] = m2l_fma(D[37], m, L[6]);
+      L[7] = m2l_fma(D[38], m, L[7]);
+      L[8] = m2l_fma(D[39], m, L[8]);
+      L[9] = m2l_fma(D[40], m, L[9]);
+      L[10] = m2l_fma(D[56], m, L[10]);
+      L[11] = m2l_fma(D[57], m, L[11]);
+      L[12] = m2l_fma(D[58], m, L[12]);
+      L[13] = m2l_fma(D[59], m, L[13]);
+      L[14] = m2l_fma(D[60], m, L[14]);
+      L[15] = m2l_fma(D[61], m, L[15]);
+      L[16] = m2l_fma(D[62], m, L[16]);
+      L[17] = m2l_fma(D[63], m, L[17]);
+      L[18] = m2l_fma(D[64], m, L[18]);
+      L[19] = m2l_fma(D[65], m, L[19]);
     }
-    { const float m = -__ldg(Ms + 36) * rp;
-      L[0] = fmaf(D[36], m, L[0]);
-      L[1] = fmaf(D[57], m, L[1]);
-      L[2] = fmaf(D[59], m, L[2]);
-      L[3] = fmaf(D[60], m, L[3]);
+    { const T m = -__ldg(Ms + 11) * rp;
+      L[0] = m2l_fma(D[11], m, L[0]);
+      L[1] = m2l_fma(D[21], m, L[1]);
+      L[2] = m2l_fma(D[23], m, L[2]);
+      L[3] = m2l_fma(D[24], m, L[3]);
+      L[4] = m2l_fma(D[36], m, L[4]);
+      L[5] = m2l_fma(D[38], m, L[5]);
+      L[6] = m2l_fma(D[39], m, L[6]);
+      L[7] = m2l_fma(D[41], m, L[7]);
+      L[8] = m2l_fma(D[42], m, L[8]);
+      L[9] = m2l_fma(D[43], m, L[9]);
+      L[10] = m2l_fma(D[57], m, L[10]);
+      L[11] = m2l_fma(D[59], m, L[11]);
+      L[12] = m2l_fma(D[60], m, L[12]);
+      L[13] = m2l_fma(D[62], m, L[13]);
+      L[14] = m2l_fma(D[63], m, L[14]);
+      L[15] = m2l_fma(D[64], m, L[15]);
+      L[16] = m2l_fma(D[66], m, L[16]);
+      L[17] = m2l_fma(D[67], m, L[17]);
+      L[18] = m2l_fma(D[68], m, L[18]);
+      L[19] = m2l_fma(D[69], m, L[19]);
     }
-    { const float m = -__ldg(Ms + 37) * rp;
-      L[0] = fmaf(D[37], m, L[0]);
-      L[1] = fmaf(D[58], m, L[1]);
-      L[2] = fmaf(D[60], m, L[2]);
-      L[3] = fmaf(D[61], m, L[3]);
+    { const T m = -__ldg(Ms + 12) * rp;
+      L[0] = m2l_fma(D[12], m, L[0]);
+      L[1] = m2l_fma(D[22], m, L[1]);
+      L[2] = m2l_fma(D[24], m, L[2]);
+      L[3] = m2l_fma(D[25], m, L[3]);
+      L[4] = m2l_fma(D[37], m, L[4]);
+      L[5] = m2l_fma(D[39], m, L[5]);
+      L[6] = m2l_fma(D[40], m, L[6]);
+      L[7] = m2l_fma(D[42], m, L[7]);
+      L[8] = m2l_fma(D[43], m, L[8]);
+      L[9] = m2l_fma(D[44], m, L[9]);
+      L[10] = m2l_fma(D[58], m, L[10]);
+      L[11] = m2l_fma(D[60], m, L[11]);
+      L[12] = m2l_fma(D[61], m, L[12]);
+      L[13] = m2l_fma(D[63], m, L[13]);
+      L[14] = m2l_fma(D[64], m, L[14]);
+      L[15] = m2l_fma(D[65], m, L[15]);
+      L[16] = m2l_fma(D[67], m, L[16]);
+      L[17] = m2l_fma(D[68], m, L[17]);
+      L[18] = m2l_fma(D[69], m, L[18]);
+      L[19] = m2l_fma(D[70], m, L[19]);
     }
-    { const float m = -__ldg(Ms + 38) * rp;
-      L[0] = fmaf(D[38], m, L[0]);
-      L[1] = fmaf(D[59], m, L[1]);
-      L[2] = fmaf(D[62], m, L[2]);
-      L[3] = fmaf(D[63], m, L[3]);
+    { const T m = -__ldg(Ms + 13) * rp;
+      L[0] = m2l_fma(D[13], m, L[0]);
+      L[1] = m2l_fma(D[23], m, L[1]);
+      L[2] = m2l_fma(D[26], m, L[2]);
+      L[3] = m2l_fma(D[27], m, L[3]);
+      L[4] = m2l_fma(D[38], m, L[4]);
+      L[5] = m2l_fma(D[41], m, L[5]);
+      L[6] = m2l_fma(D[42], m, L[6]);
+      L[7] = m2l_fma(D[45], m, L[7]);
+      L[8] = m2l_fma(D[46], m, L[8]);
+      L[9] = m2l_fma(D[47], m, L[9]);
+      L[10] = m2l_fma(D[59], m, L[10]);
+      L[11] = m2l_fma(D[62], m, L[11]);
+      L[12] = m2l_fma(D[63], m, L[12]);
+      L[13] = m2l_fma(D[66], m, L[13]);
+      L[14] = m2l_fma(D[67], m, L[14]);
+      L[15] = m2l_fma(D[68], m, L[15]);
+      L[16] = m2l_fma(D[71], m, L[16]);
+      L[17] = m2l_fma(D[72], m, L[17]);
+      L[18] = m2l_fma(D[73], m, L[18]);
+      L[19] = m2l_fma(D[74], m, L[19]);
     }
-    { const float m = -__ldg(Ms + 39) * rp;
-      L[0] = fmaf(D[39], m, L[0]);
-      L[1] = fmaf(D[60], m, L[1]);
-      L[2] = fmaf(D[63], m, L[2]);
-      L[3] = fmaf(D[64], m, L[3]);
+    { const T m = -__ldg(Ms + 14) * rp;
+      L[0] = m2l_fma(D[14], m, L[0]);
+      L[1] = m2l_fma(D[24], m, L[1]);
+      L[2] = m2l_fma(D[27], m, L[2]);
+      L[3] = m2l_fma(D[28], m, L[3]);
+      L[4] = m2l_fma(D[39], m, L[4]);
+      L[5] = m2l_fma(D[42], m, L[5]);
+      L[6] = m2l_fma(D[43], m, L[6]);
+      L[7] = m2l_fma(D[46], m, L[7]);
+      L[8] = m2l_fma(D[47], m, L[8]);
+      L[9] = m2l_fma(D[48], m, L[9]);
+      L[10] = m2l_fma(D[60], m, L[10]);
+      L[11] = m2l_fma(D[63], m, L[11]);
+      L[12] = m2l_fma(D[64], m, L[12]);
+      L[13] = m2l_fma(D[67], m, L[13]);
+      L[14] = m2l_fma(D[68], m, L[14]);
+      L[15] = m2l_fma(D[69], m, L[15]);
+      L[16] = m2l_fma(D[72], m, L[16]);
+      L[17] = m2l_fma(D[73], m, L[17]);
+      L[18] = m2l_fma(D[74], m, L[18]);
+      L[19] = m2l_fma(D[75], m, L[19]);
     }
-    { const float m = -__ldg(Ms + 40) * rp;
-      L[0] = fmaf(D[40], m, L[0]);
-      L[1] = fmaf(D[61], m, L[1]);
-      L[2] = fmaf(D[64], m, L[2]);
-      L[3] = fmaf(D[65], m, L[3]);
+    { const T m = -__ldg(Ms + 15) * rp;
+      L[0] = m2l_fma(D[15], m, L[0]);
+      L[1] = m2l_fma(D[25], m, L[1]);
+      L[2] = m2l_fma(D[28], m, L[2]);
+      L[3] = m2l_fma(D[29], m, L[3]);
+      L[4] = m2l_fma(D[40], m, L[4]);
+      L[5] = m2l_fma(D[43], m, L[5]);
+      L[6] = m2l_fma(D[44], m, L[6]);
+      L[7] = m2l_fma(D[47], m, L[7]);
+      L[8] = m2l_fma(D[48], m, L[8]);
+      L[9] = m2l_fma(D[49], m, L[9]);
+      L[10] = m2l_fma(D[61], m, L[10]);
+      L[11] = m2l_fma(D[64], m, L[11]);
+      L[12] = m2l_fma(D[65], m, L[12]);
+      L[13] = m2l_fma(D[68], m, L[13]);
+      L[14] = m2l_fma(D[69], m, L[14]);
+      L[15] = m2l_fma(D[70], m, L[15]);
+      L[16] = m2l_fma(D[73], m, L[16]);
+      L[17] = m2l_fma(D[74], m, L[17]);
+      L[18] = m2l_fma(D[75], m, L[18]);
+      L[19] = m2l_fma(D[76], m, L[19]);
     }
-    { const float m = -__ldg(Ms + 41) * rp;
-      L[0] = fmaf(D[41], m, L[0]);
-      L[1] = fmaf(D[62], m, L[1]);
-      L[2] = fmaf(D[66], m, L[2]);
-      L[3] = fmaf(D[67], m, L[3]);
+    { const T m = -__ldg(Ms + 16) * rp;
+      L[0] = m2l_fma(D[16], m, L[0]);
+      L[1] = m2l_fma(D[26], m, L[1]);
+      L[2] = m2l_fma(D[30], m, L[2]);
+      L[3] = m2l_fma(D[31], m, L[3]);
+      L[4] = m2l_fma(D[41], m, L[4]);
+      L[5] = m2l_fma(D[45], m, L[5]);
+      L[6] = m2l_fma(D[46], m, L[6]);
+      L[7] = m2l_fma(D[50], m, L[7]);
+      L[8] = m2l_fma(D[51], m, L[8]);
+      L[9] = m2l_fma(D[52], m, L[9]);
+      L[10] = m2l_fma(D[62], m, L[10]);
+      L[11] = m2l_fma(D[66], m, L[11]);
+      L[12] = m2l_fma(D[67], m, L[12]);
+      L[13] = m2l_fma(D[71], m, L[13]);
+      L[14] = m2l_fma(D[72], m, L[14]);
+      L[15] = m2l_fma(D[73], m, L[15]);
+      L[16] = m2l_fma(D[77], m, L[16]);
+      L[17] = m2l_fma(D[78], m, L[17]);
+      L[18] = m2l_fma(D[79], m, L[18]);
+      L[19] = m2l_fma(D[80], m, L[19]);
     }
-    { const float m = -__ldg(Ms + 42) * rp;
-      L[0] = fmaf(D[42], m, L[0]);
-      L[1] = fmaf(D[63], m, L[1]);
-      L[2] = fmaf(D[67], m, L[2]);
-      L[3] = fmaf(D[68], m, L[3]);
+    { const T m = -__ldg(Ms + 17) * rp;
+      L[0] = m2l_fma(D[17], m, L[0]);
+      L[1] = m2l_fma(D[27], m, L[1]);
+      L[2] = m2l_fma(D[31], m, L[2]);
+      L[3] = m2l_fma(D[32], m, L[3]);
+      L[4] = m2l_fma(D[42], m, L[4]);
+      L[5] = m2l_fma(D[46], m, L[5]);
+      L[6] = m2l_fma(D[47], m, L[6]);
+      L[7] = m2l_fma(D[51], m, L[7]);
+      L[8] = m2l_fma(D[52], m, L[8]);
+      L[9] = m2l_fma(D[53], m, L[9]);
+      L[10] = m2l_fma(D[63], m, L[10]);
+      L[11] = m2l_fma(D[67], m, L[11]);
+      L[12] = m2l_fma(D[68], m, L[12]);
+      L[13] = m2l_fma(D[72], m, L[13]);
+      L[14] = m2l_fma(D[73], m, L[14]);
+      L[15] = m2l_fma(D[74], m, L[15]);
+      L[16] = m2l_fma(D[78], m, L[16]);
+      L[17] = m2l_fma(D[79], m, L[17]);
+      L[18] = m2l_fma(D[80], m, L[18]);
+      L[19] = m2l_fma(D[81], m, L[19]);
     }
-    { const float m = -__ldg(Ms + 43) * rp;
-      L[0] = fmaf(D[43], m, L[0]);
-      L[1] = fmaf(D[64], m, L[1]);
-      L[2] = fmaf(D[68], m, L[2]);
-      L[3] = fmaf(D[69], m, L[3]);
+    { const T m = -__ldg(Ms + 18) * rp;
+      L[0] = m2l_fma(D[18], m, L[0]);
+      L[1] = m2l_fma(D[28], m, L[1]);
+      L[2] = m2l_fma(D[32], m, L[2]);
+      L[3] = m2l_fma(D[33], m, L[3]);
+      L[4] = m2l_fma(D[43], m, L[4]);
+      L[5] = m2l_fma(D[47], m, L[5]);
+      L[6] = m2l_fma(D[48], m, L[6]);
+      L[7] = m2l_fma(D[52], m, L[7]);
+      L[8] = m2l_fma(D[53], m, L[8]);
+      L[9] = m2l_fma(D[54], m, L[9]);
+      L[10] = m2l_fma(D[64], m, L[10]);
+      L[11] = m2l_fma(D[68], m, L[11]);
+      L[12] = m2l_fma(D[69], m, L[12]);
+      L[13] = m2l_fma(D[73], m, L[13]);
+      L[14] = m2l_fma(D[74], m, L[14]);
+      L[15] = m2l_fma(D[75], m, L[15]);
+      L[16] = m2l_fma(D[79], m, L[16]);
+      L[17] = m2l_fma(D[80], m, L[17]);
+      L[18] = m2l_fma(D[81], m, L[18]);
+      L[19] = m2l_fma(D[82], m, L[19]);
     }
-    { const float m = -__ldg(Ms + 44) * rp;
-      L[0] = fmaf(D[44], m, L[0]);
-      L[1] = fmaf(D[65], m, L[1]);
-      L[2] = fmaf(D[69], m, L[2]);
-      L[3] = fmaf(D[70], m, L[3]);
-    }
-    { const float m = -__ldg(Ms + 45) * rp;
-      L[0] = fmaf(D[45], m, L[0]);
-      L[1] = fmaf(D[66], m, L[1]);
-      L[2] = fmaf(D[71], m, L[2]);
-      L[3] = fmaf(D[72], m, L[3]);
-    }
-    { const float m = -__ldg(Ms + 46) * rp;
-      L[0] = fmaf(D[46], m, L[0]);
-      L[1] = fmaf(D[67], m, L[1]);
-      L[2] = fmaf(D[72], m, L[2]);
-      L[3] = fmaf(D[73], m, L[3]);
-    }
-    { const float m = -__ldg(Ms + 47) * rp;
-      L[0] = fmaf(D[47], m, L[0]);
-      L[1] = fmaf(D[68], m, L[1]);
-      L[2] = fmaf(D[73], m, L[2]);
-      L[3] = fmaf(D[74], m, L[3]);
-    }
-    { const float m = -__ldg(Ms + 48) * rp;
-      L[0] = fmaf(D[48], m, L[0]);
-      L[1] = fmaf(D[69], m, L[1]);
-      L[2] = fmaf(D[74], m, L[2]);
-      L[3] = fmaf(D[75], m, L[3]);
-    }
-    { const float m = -__ldg(Ms + 49) * rp;
-      L[0] = fmaf(D[49], m, L[0]);
-      L[1] = fmaf(D[70], m, L[1]);
-      L[2] = fmaf(D[75], m, L[2]);
-      L[3] = fmaf(D[76], m, L[3]);
-    }
-    { const float m = -__ldg(Ms + 50) * rp;
-      L[0] = fmaf(D[50], m, L[0]);
-      L[1] = fmaf(D[71], m, L[1]);
-      L[2] = fmaf(D[77], m, L[2]);
-      L[3] = fmaf(D[78], m, L[3]);
-    }
-    { const float m = -__ldg(Ms + 51) * rp;
-      L[0] = fmaf(D[51], m, L[0]);
-      L[1] = fmaf(D[72], m, L[1]);
-      L[2] = fmaf(D[78], m, L[2]);
-      L[3] = fmaf(D[79], m, L[3]);
-    }
-    { const float m = -__ldg(Ms + 52) * rp;
-      L[0] = fmaf(D[52], m, L[0]);
-      L[1] = fmaf(D[73], m, L[1]);
-      L[2] = fmaf(D[79], m, L[2]);
-      L[3] = fmaf(D[80], m, L[3]);
-    }
-    { const float m = -__ldg(Ms + 53) * rp;
-      L[0] = fmaf(D[53], m, L[0]);
-      L[1] = fmaf(D[74], m, L[1]);
-      L[2] = fmaf(D[80], m, L[2]);
-      L[3] = fmaf(D[81], m, L[3]);
-    }
-    { const float m = -__ldg(Ms + 54) * rp;
-      L[0] = fmaf(D[54], m, L[0]);
-      L[1] = fmaf(D[75], m, L[1]);
-      L[2] = fmaf(D[81], m, L[2]);
-      L[3] = fmaf(D[82], m, L[3]);
-    }
-    { const float m = -__ldg(Ms + 55) * rp;
-      L[0] = fmaf(D[55], m, L[0]);
-      L[1] = fmaf(D[76], m, L[1]);
-      L[2] = fmaf(D[82], m, L[2]);
-      L[3] = fmaf(D[83], m, L[3]);
+    { const T m = -__ldg(Ms + 19) * rp;
+      L[0] = m2l_fma(D[19], m, L[0]);
+      L[1] = m2l_fma(D[29], m, L[1]);
+      L[2] = m2l_fma(D[33], m, L[2]);
+      L[3] = m2l_fma(D[34], m, L[3]);
+      L[4] = m2l_fma(D[44], m, L[4]);
+      L[5] = m2l_fma(D[48], m, L[5]);
+      L[6] = m2l_fma(D[49], m, L[6]);
+      L[7] = m2l_fma(D[53], m, L[7]);
+      L[8] = m2l_fma(D[54], m, L[8]);
+      L[9] = m2l_fma(D[55], m, L[9]);
+      L[10] = m2l_fma(D[65], m, L[10]);
+      L[11] = m2l_fma(D[69], m, L[11]);
+      L[12] = m2l_fma(D[70], m, L[12]);
+      L[13] = m2l_fma(D[74], m, L[13]);
+      L[14] = m2l_fma(D[75], m, L[14]);
+      L[15] = m2l_fma(D[76], m, L[15]);
+      L[16] = m2l_fma(D[80], m, L[16]);
+      L[17] = m2l_fma(D[81], m, L[17]);
+      L[18] = m2l_fma(D[82], m, L[18]);
+      L[19] = m2l_fma(D[83], m, L[19]);
     }
     rp *= rho;
-    { const float m = __ldg(Ms + 56) * rp;
-      L[0] = fmaf(D[56], m, L[0]);
+    { const T m = __ldg(Ms + 20) * rp;
+      L[0] = m2l_fma(D[20], m, L[0]);
+      L[1] = m2l_fma(D[35], m, L[1]);
+      L[2] = m2l_fma(D[36], m, L[2]);
+      L[3] = m2l_fma(D[37], m, L[3]);
+      L[4] = m2l_fma(D[56], m, L[4]);
+      L[5] = m2l_fma(D[57], m, L[5]);
+      L[6] = m2l_fma(D[58], m, L[6]);
+      L[7] = m2l_fma(D[59], m, L[7]);
+      L[8] = m2l_fma(D[60], m, L[8]);
+      L[9] = m2l_fma(D[61], m, L[9]);
     }
-    { const float m = __ldg(Ms + 57) * rp;
-      L[0] = fmaf(D[57], m, L[0]);
+    { const T m = __ldg(Ms + 21) * rp;
+      L[0] = m2l_fma(D[21], m, L[0]);
+      L[1] = m2l_fma(D[36], m, L[1]);
+      L[2] = m2l_fma(D[38], m, L[2]);
+      L[3] = m2l_fma(D[39], m, L[3]);
+      L[4] = m2l_fma(D[57], m, L[4]);
+      L[5] = m2l_fma(D[59], m, L[5]);
+      L[6] = m2l_fma(D[60], m, L[6]);
+      L[7] = m2l_fma(D[62], m, L[7]);
+      L[8] = m2l_fma(D[63], m, L[8]);
+      L[9] = m2l_fma(D[64], m, L[9]);
     }
-    { const float m = __ldg(Ms + 58) * rp;
-      L[0] = fmaf(D[58], m, L[0]);
+    { const T m = __ldg(Ms + 22) * rp;
+      L[0] = m2l_fma(D[22], m, L[0]);
+      L[1] = m2l_fma(D[37], m, L[1]);
+      L[2] = m2l_fma(D[39], m, L[2]);
+      L[3] = m2l_fma(D[40], m, L[3]);
+      L[4] = m2l_fma(D[58], m, L[4]);
+      L[5] = m2l_fma(D[60], m, L[5]);
+      L[6] = m2l_fma(D[61], m, L[6]);
+      L[7] = m2l_fma(D[63], m, L[7]);
+      L[8] = m2l_fma(D[64], m, L[8]);
+      L[9] = m2l_fma(D[65], m, L[9]);
     }
-    { const float m = __ldg(Ms + 59) * rp;
-      L[0] = fmaf(D[59], m, L[0]);
+    { const T m = __ldg(Ms + 23) * rp;
+      L[0] = m2l_fma(D[23], m, L[0]);
+      L[1] = m2l_fma(D[38], m, L[1]);
+      L[2] = m2l_fma(D[41], m, L[2]);
+      L[3] = m2l_fma(D[42], m, L[3]);
+      L[4] = m2l_fma(D[59], m, L[4]);
+      L[5] = m2l_fma(D[62], m, L[5]);
+      L[6] = m2l_fma(D[63], m, L[6]);
+      L[7] = m2l_fma(D[66], m, L[7]);
+      L[8] = m2l_fma(D[67], m, L[8]);
+      L[9] = m2l_fma(D[68], m, L[9]);
     }
-    { const float m = __ldg(Ms + 60) * rp;
-      L[0] = fmaf(D[60], m, L[0]);
+    { const T m = __ldg(Ms + 24) * rp;
+      L[0] = m2l_fma(D[24], m, L[0]);
+      L[1] = m2l_fma(D[39], m, L[1]);
+      L[2] = m2l_fma(D[42], m, L[2]);
+      L[3] = m2l_fma(D[43], m, L[3]);
+      L[4] = m2l_fma(D[60], m, L[4]);
+      L[5] = m2l_fma(D[63], m, L[5]);
+      L[6] = m2l_fma(D[64], m, L[6]);
+      L[7] = m2l_fma(D[67], m, L[7]);
+      L[8] = m2l_fma(D[68], m, L[8]);
+      L[9] = m2l_fma(D[69], m, L[9]);
     }
-    { const float m = __ldg(Ms + 61) * rp;
-      L[0] = fmaf(D[61], m, L[0]);
+    { const T m = __ldg(Ms + 25) * rp;
+      L[0] = m2l_fma(D[25], m, L[0]);
+      L[1] = m2l_fma(D[40], m, L[1]);
+      L[2] = m2l_fma(D[43], m, L[2]);
+      L[3] = m2l_fma(D[44], m, L[3]);
+      L[4] = m2l_fma(D[61], m, L[4]);
+      L[5] = m2l_fma(D[64], m, L[5]);
+      L[6] = m2l_fma(D[65], m, L[6]);
+      L[7] = m2l_fma(D[68], m, L[7]);
+      L[8] = m2l_fma(D[69], m, L[8]);
+      L[9] = m2l_fma(D[70], m, L[9]);
     }
-    { const float m = __ldg(Ms + 62) * rp;
-      L[0] = fmaf(D[62], m, L[0]);
+    { const T m = __ldg(Ms + 26) * rp;
+      L[0] = m2l_fma(D[26], m, L[0]);
+      L[1] = m2l_fma(D[41], m, L[1]);
+      L[2] = m2l_fma(D[45], m, L[2]);
+      L[3] = m2l_fma(D[46], m, L[3]);
+      L[4] = m2l_fma(D[62], m, L[4]);
+      L[5] = m2l_fma(D[66], m, L[5]);
+      L[6] = m2l_fma(D[67], m, L[6]);
+      L[7] = m2l_fma(D[71], m, L[7]);
+      L[8] = m2l_fma(D[72], m, L[8]);
+      L[9] = m2l_fma(D[73], m, L[9]);
     }
-    { const float m = __ldg(Ms + 63) * rp;
-      L[0] = fmaf(D[63], m, L[0]);
+    { const T m = __ldg(Ms + 27) * rp;
+      L[0] = m2l_fma(D[27], m, L[0]);
+      L[1] = m2l_fma(D[42], m, L[1]);
+      L[2] = m2l_fma(D[46], m, L[2]);
+      L[3] = m2l_fma(D[47], m, L[3]);
+      L[4] = m2l_fma(D[63], m, L[4]);
+      L[5] = m2l_fma(D[67], m, L[5]);
+      L[6] = m2l_fma(D[68], m, L[6]);
+      L[7] = m2l_fma(D[72], m, L[7]);
+      L[8] = m2l_fma(D[73], m, L[8]);
+      L[9] = m2l_fma(D[74], m, L[9]);
     }
-    { const float m = __ldg(Ms + 64) * rp;
-      L[0] = fmaf(D[64], m, L[0]);
+    { const T m = __ldg(Ms + 28) * rp;
+      L[0] = m2l_fma(D[28], m, L[0]);
+      L[1] = m2l_fma(D[43], m, L[1]);
+      L[2] = m2l_fma(D[47], m, L[2]);
+      L[3] = m2l_fma(D[48], m, L[3]);
+      L[4] = m2l_fma(D[64], m, L[4]);
+      L[5] = m2l_fma(D[68], m, L[5]);
+      L[6] = m2l_fma(D[69], m, L[6]);
+      L[7] = m2l_fma(D[73], m, L[7]);
+      L[8] = m2l_fma(D[74], m, L[8]);
+      L[9] = m2l_fma(D[75], m, L[9]);
     }
-    { const float m = __ldg(Ms + 65) * rp;
-      L[0] = fmaf(D[65], m, L[0]);
+    { const T m = __ldg(Ms + 29) * rp;
+      L[0] = m2l_fma(D[29], m, L[0]);
+      L[1] = m2l_fma(D[44], m, L[1]);
+      L[2] = m2l_fma(D[48], m, L[2]);
+      L[3] = m2l_fma(D[49], m, L[3]);
+      L[4] = m2l_fma(D[65], m, L[4]);
+      L[5] = m2l_fma(D[69], m, L[5]);
+      L[6] = m2l_fma(D[70], m, L[6]);
+      L[7] = m2l_fma(D[74], m, L[7]);
+      L[8] = m2l_fma(D[75], m, L[8]);
+      L[9] = m2l_fma(D[76], m, L[9]);
     }
-    { const float m = __ldg(Ms + 66) * rp;
-      L[0] = fmaf(D[66], m, L[0]);
+    { const T m = __ldg(Ms + 30) * rp;
+      L[0] = m2l_fma(D[30], m, L[0]);
+      L[1] = m2l_fma(D[45], m, L[1]);
+      L[2] = m2l_fma(D[50], m, L[2]);
+      L[3] = m2l_fma(D[51], m, L[3]);
+      L[4] = m2l_fma(D[66], m, L[4]);
+      L[5] = m2l_fma(D[71], m, L[5]);
+      L[6] = m2l_fma(D[72], m, L[6]);
+      L[7] = m2l_fma(D[77], m, L[7]);
+      L[8] = m2l_fma(D[78], m, L[8]);
+      L[9] = m2l_fma(D[79], m, L[9]);
     }
-    { const float m = __ldg(Ms + 67) * rp;
-      L[0] = fmaf(D[67], m, L[0]);
+    { const T m = __ldg(Ms + 31) * rp;
+      L[0] = m2l_fma(D[31], m, L[0]);
+      L[1] = m2l_fma(D[46], m, L[1]);
+      L[2] = m2l_fma(D[51], m, L[2]);
+      L[3] = m2l_fma(D[52], m, L[3]);
+      L[4] = m2l_fma(D[67], m, L[4]);
+      L[5] = m2l_fma(D[72], m, L[5]);
+      L[6] = m2l_fma(D[73], m, L[6]);
+      L[7] = m2l_fma(D[78], m, L[7]);
+      L[8] = m2l_fma(D[79], m, L[8]);
+      L[9] = m2l_fma(D[80], m, L[9]);
     }
-    { const float m = __ldg(Ms + 68) * rp;
-      L[0] = fmaf(D[68], m, L[0]);
+    { const T m = __ldg(Ms + 32) * rp;
+      L[0] = m2l_fma(D[32], m, L[0]);
+      L[1] = m2l_fma(D[47], m, L[1]);
+      L[2] = m2l_fma(D[52], m, L[2]);
+      L[3] = m2l_fma(D[53], m, L[3]);
+      L[4] = m2l_fma(D[68], m, L[4]);
+      L[5] = m2l_fma(D[73], m, L[5]);
+      L[6] = m2l_fma(D[74], m, L[6]);
+      L[7] = m2l_fma(D[79], m, L[7]);
+      L[8] = m2l_fma(D[80], m, L[8]);
+      L[9] = m2l_fma(D[81], m, L[9]);
     }
-    { const float m = __ldg(Ms + 69) * rp;
-      L[0] = fmaf(D[69], m, L[0]);
+    { const T m = __ldg(Ms + 33) * rp;
+      L[0] = m2l_fma(D[33], m, L[0]);
+      L[1] = m2l_fma(D[48], m, L[1]);
+      L[2] = m2l_fma(D[53], m, L[2]);
+      L[3] = m2l_fma(D[54], m, L[3]);
+      L[4] = m2l_fma(D[69], m, L[4]);
+      L[5] = m2l_fma(D[74], m, L[5]);
+      L[6] = m2l_fma(D[75], m, L[6]);
+      L[7] = m2l_fma(D[80], m, L[7]);
+      L[8] = m2l_fma(D[81], m, L[8]);
+      L[9] = m2l_fma(D[82], m, L[9]);
     }
-    { const float m = __ldg(Ms + 70) * rp;
-      L[0] = fmaf(D[70], m, L[0]);
+    { const T m = __ldg(Ms + 34) * rp;
+      L[0] = m2l_fma(D[34], m, L[0]);
+      L[1] = m2l_fma(D[49], m, L[1]);
+      L[2] = m2l_fma(D[54], m, L[2]);
+      L[3] = m2l_fma(D[55], m, L[3]);
+      L[4] = m2l_fma(D[70], m, L[4]);
+      L[5] = m2l_fma(D[75], m, L[5]);
+      L[6] = m2l_fma(D[76], m, L[6]);
+      L[7] = m2l_fma(D[81], m, L[7]);
+      L[8] = m2l_fma(D[82], m, L[8]);
+      L[9] = m2l_fma(D[83], m, L[9]);
     }
-    { const float m = __ldg(Ms + 71) * rp;
-      L[0] = fmaf(D[71], m, L[0]);
+    rp *= rho;
+    { const T m = -__ldg(Ms + 35) * rp;
+      L[0] = m2l_fma(D[35], m, L[0]);
+      L[1] = m2l_fma(D[56], m, L[1]);
+      L[2] = m2l_fma(D[57], m, L[2]);
+      L[3] = m2l_fma(D[58], m, L[3]);
     }
-    { const float m = __ldg(Ms + 72) * rp;
-      L[0] = fmaf(D[72], m, L[0]);
+    { const T m = -__ldg(Ms + 36) * rp;
+      L[0] = m2l_fma(D[36], m, L[0]);
+      L[1] = m2l_fma(D[57], m, L[1]);
+      L[2] = m2l_fma(D[59], m, L[2]);
+      L[3] = m2l_fma(D[60], m, L[3]);
     }
-    { const float m = __ldg(Ms + 73) * rp;
-      L[0] = fmaf(D[73], m, L[0]);
+    { const T m = -__ldg(Ms + 37) * rp;
+      L[0] = m2l_fma(D[37], m, L[0]);
+      L[1] = m2l_fma(D[58], m, L[1]);
+      L[2] = m2l_fma(D[60], m, L[2]);
+      L[3] = m2l_fma(D[61], m, L[3]);
     }
-    { const float m = __ldg(Ms + 74) * rp;
-      L[0] = fmaf(D[74], m, L[0]);
+    { const T m = -__ldg(Ms + 38) * rp;
+      L[0] = m2l_fma(D[38], m, L[0]);
+      L[1] = m2l_fma(D[59], m, L[1]);
+      L[2] = m2l_fma(D[62], m, L[2]);
+      L[3] = m2l_fma(D[63], m, L[3]);
     }
-    { const float m = __ldg(Ms + 75) * rp;
-      L[0] = fmaf(D[75], m, L[0]);
+    { const T m = -__ldg(Ms + 39) * rp;
+      L[0] = m2l_fma(D[39], m, L[0]);
+      L[1] = m2l_fma(D[60], m, L[1]);
+      L[2] = m2l_fma(D[63], m, L[2]);
+      L[3] = m2l_fma(D[64], m, L[3]);
     }
-    { const float m = __ldg(Ms + 76) * rp;
-      L[0] = fmaf(D[76], m, L[0]);
+    { const T m = -__ldg(Ms + 40) * rp;
+      L[0] = m2l_fma(D[40], m, L[0]);
+      L[1] = m2l_fma(D[61], m, L[1]);
+      L[2] = m2l_fma(D[64], m, L[2]);
+      L[3] = m2l_fma(D[65], m, L[3]);
     }
-    { const float m = __ldg(Ms + 77) * rp;
-      L[0] = fmaf(D[77], m, L[0]);
+    { const T m = -__ldg(Ms + 41) * rp;
+      L[0] = m2l_fma(D[41], m, L[0]);
+      L[1] = m2l_fma(D[62], m, L[1]);
+      L[2] = m2l_fma(D[66], m, L[2]);
+      L[3] = m2l_fma(D[67], m, L[3]);
     }
-    { const float m = __ldg(Ms + 78) * rp;
-      L[0] = fmaf(D[78], m, L[0]);
+    { const T m = -__ldg(Ms + 42) * rp;
+      L[0] = m2l_fma(D[42], m, L[0]);
+      L[1] = m2l_fma(D[63], m, L[1]);
+      L[2] = m2l_fma(D[67], m, L[2]);
+      L[3] = m2l_fma(D[68], m, L[3]);
     }
-    { const float m = __ldg(Ms + 79) * rp;
-      L[0] = fmaf(D[79], m, L[0]);
+    { const T m = -__ldg(Ms + 43) * rp;
+      L[0] = m2l_fma(D[43], m, L[0]);
+      L[1] = m2l_fma(D[64], m, L[1]);
+      L[2] = m2l_fma(D[68], m, L[2]);
+      L[3] = m2l_fma(D[69], m, L[3]);
     }
-    { const float m = __ldg(Ms + 80) * rp;
-      L[0] = fmaf(D[80], m, L[0]);
+    { const T m = -__ldg(Ms + 44) * rp;
+      L[0] = m2l_fma(D[44], m, L[0]);
+      L[1] = m2l_fma(D[65], m, L[1]);
+      L[2] = m2l_fma(D[69], m, L[2]);
+      L[3] = m2l_fma(D[70], m, L[3]);
     }
-    { const float m = __ldg(Ms + 81) * rp;
-      L[0] = fmaf(D[81], m, L[0]);
+    { const T m = -__ldg(Ms + 45) * rp;
+      L[0] = m2l_fma(D[45], m, L[0]);
+      L[1] = m2l_fma(D[66], m, L[1]);
+      L[2] = m2l_fma(D[71], m, L[2]);
+      L[3] = m2l_fma(D[72], m, L[3]);
     }
-    { const float m = __ldg(Ms + 82) * rp;
-      L[0] = fmaf(D[82], m, L[0]);
+    { const T m = -__ldg(Ms + 46) * rp;
+      L[0] = m2l_fma(D[46], m, L[0]);
+      L[1] = m2l_fma(D[67], m, L[1]);
+      L[2] = m2l_fma(D[72], m, L[2]);
+      L[3] = m2l_fma(D[73], m, L[3]);
     }
-    { const float m = __ldg(Ms + 83) * rp;
-      L[0] = fmaf(D[83], m, L[0]);
+    { const T m = -__ldg(Ms + 47) * rp;
+      L[0] = m2l_fma(D[47], m, L[0]);
+      L[1] = m2l_fma(D[68], m, L[1]);
+      L[2] = m2l_fma(D[73], m, L[2]);
+      L[3] = m2l_fma(D[74], m, L[3]);
+    }
+    { const T m = -__ldg(Ms + 48) * rp;
+      L[0] = m2l_fma(D[48], m, L[0]);
+      L[1] = m2l_fma(D[69], m, L[1]);
+      L[2] = m2l_fma(D[74], m, L[2]);
+      L[3] = m2l_fma(D[75], m, L[3]);
+    }
+    { const T m = -__ldg(Ms + 49) * rp;
+      L[0] = m2l_fma(D[49], m, L[0]);
+      L[1] = m2l_fma(D[70], m, L[1]);
+      L[2] = m2l_fma(D[75], m, L[2]);
+      L[3] = m2l_fma(D[76], m, L[3]);
+    }
+    { const T m = -__ldg(Ms + 50) * rp;
+      L[0] = m2l_fma(D[50], m, L[0]);
+      L[1] = m2l_fma(D[71], m, L[1]);
+      L[2] = m2l_fma(D[77], m, L[2]);
+      L[3] = m2l_fma(D[78], m, L[3]);
+    }
+    { const T m = -__ldg(Ms + 51) * rp;
+      L[0] = m2l_fma(D[51], m, L[0]);
+      L[1] = m2l_fma(D[72], m, L[1]);
+      L[2] = m2l_fma(D[78], m, L[2]);
+      L[3] = m2l_fma(D[79], m, L[3]);
+    }
+    { const T m = -__ldg(Ms + 52) * rp;
+      L[0] = m2l_fma(D[52], m, L[0]);
+      L[1] = m2l_fma(D[73], m, L[1]);
+      L[2] = m2l_fma(D[79], m, L[2]);
+      L[3] = m2l_fma(D[80], m, L[3]);
+    }
+    { const T m = -__ldg(Ms + 53) * rp;
+      L[0] = m2l_fma(D[53], m, L[0]);
+      L[1] = m2l_fma(D[74], m, L[1]);
+      L[2] = m2l_fma(D[80], m, L[2]);
+      L[3] = m2l_fma(D[81], m, L[3]);
+    }
+    { const T m = -__ldg(Ms + 54) * rp;
+      L[0] = m2l_fma(D[54], m, L[0]);
+      L[1] = m2l_fma(D[75], m, L[1]);
+      L[2] = m2l_fma(D[81], m, L[2]);
+      L[3] = m2l_fma(D[82], m, L[3]);
+    }
+    { const T m = -__ldg(Ms + 55) * rp;
+      L[0] = m2l_fma(D[55], m, L[0]);
+      L[1] = m2l_fma(D[76], m, L[1]);
+      L[2] = m2l_fma(D[82], m, L[2]);
+      L[3] = m2l_fma(D[83], m, L[3]);
+    }
+    rp *= rho;
+    { const T m = __ldg(Ms + 56) * rp;
+      L[0] = m2l_fma(D[56], m, L[0]);
+    }
+    { const T m = __ldg(Ms + 57) * rp;
+      L[0] = m2l_fma(D[57], m, L[0]);
+    }
+    { const T m = __ldg(Ms + 58) * rp;
+      L[0] = m2l_fma(D[58], m, L[0]);
+    }
+    { const T m = __ldg(Ms + 59) * rp;
+      L[0] = m2l_fma(D[59], m, L[0]);
+    }
+    { const T m = __ldg(Ms + 60) * rp;
+      L[0] = m2l_fma(D[60], m, L[0]);
+    }
+    { const T m = __ldg(Ms + 61) * rp;
+      L[0] = m2l_fma(D[61], m, L[0]);
+    }
+    { const T m = __ldg(Ms + 62) * rp;
+      L[0] = m2l_fma(D[62], m, L[0]);
+    }
+    { const T m = __ldg(Ms + 63) * rp;
+      L[0] = m2l_fma(D[63], m, L[0]);
+    }
+    { const T m = __ldg(Ms + 64) * rp;
+      L[0] = m2l_fma(D[64], m, L[0]);
+    }
+    { const T m = __ldg(Ms + 65) * rp;
+      L[0] = m2l_fma(D[65], m, L[0]);
+    }
+    { const T m = __ldg(Ms + 66) * rp;
+      L[0] = m2l_fma(D[66], m, L[0]);
+    }
+    { const T m = __ldg(Ms + 67) * rp;
+      L[0] = m2l_fma(D[67], m, L[0]);
+    }
+    { const T m = __ldg(Ms + 68) * rp;
+      L[0] = m2l_fma(D[68], m, L[0]);
+    }
+    { const T m = __ldg(Ms + 69) * rp;
+      L[0] = m2l_fma(D[69], m, L[0]);
+    }
+    { const T m = __ldg(Ms + 70) * rp;
+      L[0] = m2l_fma(D[70], m, L[0]);
+    }
+    { const T m = __ldg(Ms + 71) * rp;
+      L[0] = m2l_fma(D[71], m, L[0]);
+    }
+    { const T m = __ldg(Ms + 72) * rp;
+      L[0] = m2l_fma(D[72], m, L[0]);
+    }
+    { const T m = __ldg(Ms + 73) * rp;
+      L[0] = m2l_fma(D[73], m, L[0]);
+    }
+    { const T m = __ldg(Ms + 74) * rp;
+      L[0] = m2l_fma(D[74], m, L[0]);
+    }
+    { const T m = __ldg(Ms + 75) * rp;
+      L[0] = m2l_fma(D[75], m, L[0]);
+    }
+    { const T m = __ldg(Ms + 76) * rp;
+      L[0] = m2l_fma(D[76], m, L[0]);
+    }
+    { const T m = __ldg(Ms + 77) * rp;
+      L[0] = m2l_fma(D[77], m, L[0]);
+    }
+    { const T m = __ldg(Ms + 78) * rp;
+      L[0] = m2l_fma(D[78], m, L[0]);
+    }
+    { const T m = __ldg(Ms + 79) * rp;
+      L[0] = m2l_fma(D[79], m, L[0]);
+    }
+    { const T m = __ldg(Ms + 80) * rp;
+      L[0] = m2l_fma(D[80], m, L[0]);
+    }
+    { const T m = __ldg(Ms + 81) * rp;
+      L[0] = m2l_fma(D[81], m, L[0]);
+    }
+    { const T m = __ldg(Ms + 82) * rp;
+      L[0] = m2l_fma(D[82], m, L[0]);
+    }
+    { const T m = __ldg(Ms + 83) * rp;
+      L[0] = m2l_fma(D[83], m, L[0]);
     }
 }
 
-__device__ __forceinline__ void m2l_side_b_6(const float (&D)[84], const float *__restrict__ Ms, float (&L)[84])
+template <class T> __device__ __forceinline__ void m2l_side_b_6(const T (&D)[84], const T *__restrict__ Ms, T (&L)[84])
 {
-    { const float m = __ldg(Ms + 0);
+    { const T m = __ldg(Ms + 0);
       L[0] = D[0] * m;
       L[1] = -D[1] * m;
       L[2] = -D[2] * m;
@@ -5756,1019 +5761,1019 @@ __device__ __forceinline__ void m2l_side_b_6(const float (&D)[84], const float *
       L[82] = D[82] * m;
       L[83] = D[83] * m;
     }
-    { const float m = __ldg(Ms + 1);
-      L[0] = fmaf(D[1], m, L[0]);
-      L[1] = fmaf(-D[4], m, L[1]);
-      L[2] = fmaf(-D[5], m, L[2]);
-      L[3] = fmaf(-D[6], m, L[3]);
-      L[4] = fmaf(D[10], m, L[4]);
-      L[5] = fmaf(D[11], m, L[5]);
-      L[6] = fmaf(D[12], m, L[6]);
-      L[7] = fmaf(D[13], m, L[7]);
-      L[8] = fmaf(D[14], m, L[8]);
-      L[9] = fmaf(D[15], m, L[9]);
-      L[10] = fmaf(-D[20], m, L[10]);
-      L[11] = fmaf(-D[21], m, L[11]);
-      L[12] = fmaf(-D[22], m, L[12]);
-      L[13] = fmaf(-D[23], m, L[13]);
-      L[14] = fmaf(-D[24], m, L[14]);
-      L[15] = fmaf(-D[25], m, L[15]);
-      L[16] = fmaf(-D[26], m, L[16]);
-      L[17] = fmaf(-D[27], m, L[17]);
-      L[18] = fmaf(-D[28], m, L[18]);
-      L[19] = fmaf(-D[29], m, L[19]);
-      L[20] = fmaf(D[35], m, L[20]);
-      L[21] = fmaf(D[36], m, L[21]);
-      L[22] = fmaf(D[37], m, L[22]);
-      L[23] = fmaf(D[38], m, L[23]);
-      L[24] = fmaf(D[39], m, L[24]);
-      L[25] = fmaf(D[40], m, L[25]);
-      L[26] = fmaf(D[41], m, L[26]);
-      L[27] = fmaf(D[42], m, L[27]);
-      L[28] = fmaf(D[43], m, L[28]);
-      L[29] = fmaf(D[44], m, L[29]);
-      L[30] = fmaf(D[45], m, L[30]);
-      L[31] = fmaf(D[46], m, L[31]);
-      L[32] = fmaf(D[47], m, L[32]);
-      L[33] = fmaf(D[48], m, L[33]);
-      L[34] = fmaf(D[49], m, L[34]);
-      L[35] = fmaf(-D[56], m, L[35]);
-      L[36] = fmaf(-D[57], m, L[36]);
-      L[37] = fmaf(-D[58], m, L[37]);
-      L[38] = fmaf(-D[59], m, L[38]);
-      L[39] = fmaf(-D[60], m, L[39]);
-      L[40] = fmaf(-D[61], m, L[40]);
-      L[41] = fmaf(-D[62], m, L[41]);
-      L[42] = fmaf(-D[63], m, L[42]);
-      L[43] = fmaf(-D[64], m, L[43]);
-      L[44] = fmaf(-D[65], m, L[44]);
-      L[45] = fmaf(-D[66], m, L[45]);
-      L[46] = fmaf(-D[67], m, L[46]);
-      L[47] = fmaf(-D[68], m, L[47]);
-      L[48] = fmaf(-D[69], m, L[48]);
-      L[49] = fmaf(-D[70], m, L[49]);
-      L[50] = fmaf(-D[71], m, L[50]);
-      L[51] = fmaf(-D[72], m, L[51]);
-      L[52] = fmaf(-D[73], m, L[52]);
-      L[53] = fmaf(-D[74], m, L[53]);
-      L[54] = fmaf(-D[75], m, L[54]);
-      L[55] = fmaf(-D[76], m, L[55]);
-    }
-    { const float m = __ldg(Ms + 2);
-      L[0] = fmaf(D[2], m, L[0]);
-      L[1] = fmaf(-D[5], m, L[1]);
-      L[2] = fmaf(-D[7], m, L[2]);
-      L[3] = fmaf(-D[8], m, L[3]);
-      L[4] = fmaf(D[11], m, L[4]);
-      L[5] = fmaf(D[13], m, L[5]);
-      L[6] = fmaf(D[14], m, L[6]);
-      L[7] = fmaf(D[16], m, L[7]);
-      L[8] = fmaf(D[17], m, L[8]);
-      L[9] = fmaf(D[18], m, L[9]);
-      L[10] = fmaf(-D[21], m, L[10]);
-      L[11] = fmaf(-D[23], m, L[11]);
-      L[12] = fmaf(-D[24], m, L[12]);
-      L[13] = fmaf(-D[26], m, L[13]);
-      L[14] = fmaf(-D[27], m, L[14]);
-      L[15] = fmaf(-D[28], m, L[15]);
-      L[16] = fmaf(-D[30], m, L[16]);
-      L[17] = fmaf(-D[31], m, L[17]);
-      L[18] = fmaf(-D[32], m, L[18]);
-      L[19] = fmaf(-D[33], m, L[19]);
-      L[20] = fmaf(D[36], m, L[20]);
-      L[21] = fmaf(D[38], m, L[21]);
-      L[22] = fmaf(D[39], m, L[22]);
-      L[23] = fmaf(D[41], m, L[23]);
-      L[24] = fmaf(D[42], m, L[24]);
-      L[25] = fmaf(D[43], m, L[25]);
-      L[26] = fmaf(D[45], m, L[26]);
-      L[27] = fmaf(D[46], m, L[27]);
-      L[28] = fmaf(D[47], m, L[28]);
-      L[29] = fmaf(D[48], m, L[29]);
-      L[30] = fmaf(D[50], m, L[30]);
-      L[31] = fmaf(D[51], m, L[31]);
-      L[32] = fmaf(D[52], m, L[32]);
-      L[33] = fmaf(D[53], m, L[33]);
-      L[34] = fmaf(D[54], m, L[34]);
-      L[35] = fmaf(-D[57], m, L[35]);
-      L[36] = fmaf(-D[59], m, L[36]);
-      L[37] = fmaf(-D[60], m, L[37]);
-      L[38] = fmaf(-D[62], m, L[38]);
-      L[39] = fmaf(-D[63], m, L[39]);
-      L[40] = fmaf(-D[64], m, L[40]);
-      L[41] = fmaf(-D[66], m, L[41]);
-      L[42] = fmaf(-D[67], m, L[42]);
-      L[43] = fmaf(-D[68], m, L[43]);
-      L[44] = fmaf(-D[69], m, L[44]);
-      L[45] = fmaf(-D[71], m, L[45]);
-      L[46] = fmaf(-D[72], m, L[46]);
-      L[47] = fmaf(-D[73], m, L[47]);
-      L[48] = fmaf(-D[74], m, L[48]);
-      L[49] = fmaf(-D[75], m, L[49]);
-      L[50] = fmaf(-D[77], m, L[50]);
-      L[51] = fmaf(-D[78], m, L[51]);
-      L[52] = fmaf(-D[79], m, L[52]);
-      L[53] = fmaf(-D[80], m, L[53]);
-      L[54] = fmaf(-D[81], m, L[54]);
-      L[55] = fmaf(-D[82], m, L[55]);
-    }
-    { const float m = __ldg(Ms + 3);
-      L[0] = fmaf(D[3], m, L[0]);
-      L[1] = fmaf(-D[6], m, L[1]);
-      L[2] = fmaf(-D[8], m, L[2]);
-      L[3] = fmaf(-D[9], m, L[3]);
-      L[4] = fmaf(D[12], m, L[4]);
-      L[5] = fmaf(D[14], m, L[5]);
-      L[6] = fmaf(D[15], m, L[6]);
-      L[7] = fmaf(D[17], m, L[7]);
-      L[8] = fmaf(D[18], m, L[8]);
-      L[9] = fmaf(D[19], m, L[9]);
-      L[10] = fmaf(-D[22], m, L[10]);
-      L[11] = fmaf(-D[24], m, L[11]);
-      L[12] = fmaf(-D[25], m, L[12]);
-      L[13] = fmaf(-D[27], m, L[13]);
-      L[14] = fmaf(-D[28], m, L[14]);
-      L[15] = fmaf(-D[29], m, L[15]);
-      L[16] = fmaf(-D[31], m, L[16]);
-      L[17] = fmaf(-D[32], m, L[17]);
-      L[18] = fmaf(-D[33], m, L[18]);
-      L[19] = fmaf(-D[34], m, L[19]);
-      L[20] = fmaf(D[37], m, L[20]);
-      L[21] = fmaf(D[39], m, L[21]);
-      L[22] = fmaf(D[40], m, L[22]);
-      L[23] = fmaf(D[42], m, L[23]);
-      L[24] = fmaf(D[43], m, L[24]);
-      L[25] = fmaf(D[44], m, L[25]);
-      L[26] = fmaf(D[46], m, L[26]);
-      L[27] = fmaf(D[47], m, L[27]);
-      L[28] = fmaf(D[48], m, L[28]);
-      L[29] = fmaf(D[49], m, L[29]);
-      L[30] = fmaf(D[51], m, L[30]);
-      L[31] = fmaf(D[52], m, L[31]);
-      L[32] = fmaf(D[53], m, L[32]);
-      L[33] = fmaf(D[54], m, L[33]);
-      L[34] = fmaf(D[55], m, L[34]);
-      L[35] = fmaf(-D[58], m, L[35]);
-      L[36] = fmaf(-D[60], m, L[36]);
-      L[37] = fmaf(-D[61], m, L[37]);
-      L[38] = fmaf(-D[63], m, L[38]);
-      L[39] = fmaf(-D[64], m, L[39]);
-      L[40] = fmaf(-D[65], m, L[40]);
-      L[41] = fmaf(-D[67], m, L[41]);
-      L[42] = fmaf(-D[68], m, L[42]);
-      L[43] = fmaf(-D[69], m, L[43]);
-      L[44] = fmaf(-D[70], m, L[44]);
-      L[45] = fmaf(-D[72], m, L[45]);
-      L[46] = fmaf(-D[73], m, L[46]);
-      L[47] = fmaf(-D[74], m, L[47]);
-      L[48] = fmaf(-D[75], m, L[48]);
-      L[49] = fmaf(-D[76], m, L[49]);
-      L[50] = fmaf(-D[78], m, L[50]);
-      L[51] = fmaf(-D[79], m, L[51]);
-      L[52] = fmaf(-D[80], m, L[52]);
-      L[53] = fmaf(-D[81], m, L[53]);
-      L[54] = fmaf(-D[82], m, L[54]);
-      L[55] = fmaf(-D[83], m, L[55]);
-    }
-    { const float m = __ldg(Ms + 4);
-      L[0] = fmaf(D[4], m, L[0]);
-      L[1] = fmaf(-D[10], m, L[1]);
-      L[2] = fmaf(-D[11], m, L[2]);
-      L[3] = fmaf(-D[12], m, L[3]);
-      L[4] = fmaf(D[20], m, L[4]);
-      L[5] = fmaf(D[21], m, L[5]);
-      L[6] = fmaf(D[22], m, L[6]);
-      L[7] = fmaf(D[23], m, L[7]);
-      L[8] = fmaf(D[24], m, L[8]);
-      L[9] = fmaf(D[25], m, L[9]);
-      L[10] = fmaf(-D[35], m, L[10]);
-      L[11] = fmaf(-D[36], m, L[11]);
-      L[12] = fmaf(-D[37], m, L[12]);
-      L[13] = fmaf(-D[38], m, L[13]);
-      L[14] = fmaf(-D[39], m, L[14]);
-      L[15] = fmaf(-D[40], m, L[15]);
-      L[16] = fmaf(-D[41], m, L[16]);
-      L[17] = fmaf(-D[42], m, L[17]);
-      L[18] = fmaf(-D[43], m, L[18]);
-      L[19] = fmaf(-D[44], m, L[19]);
-      L[20] = fmaf(D[56], m, L[20]);
-      L[21] = fmaf(D[57], m, L[21]);
-      L[22] = fmaf(D[58], m, L[22]);
-      L[23] = fmaf(D[59], m, L[23]);
-      L[24] = fmaf(D[60], m, L[24]);
-      L[25] = fmaf(D[61], m, L[25]);
-      L[26] = fmaf(D[62], m, L[26]);
-      L[27] = fmaf(D[63], m, L[27]);
-      L[28] = fmaf(D[64], m, L[28]);
-      L[29] = fmaf(D[65], m, L[29]);
-      L[30] = fmaf(D[66], m, L[30]);
-      L[31] = fmaf(D[67], m, L[31]);
-      L[32] = fmaf(D[68], m, L[32]);
-      L[33] = fmaf(D[69], m, L[33]);
-      L[34] = fmaf(D[70], m, L[34]);
-    }
-    { const float m = __ldg(Ms + 5);
-      L[0] = fmaf(D[5], m, L[0]);
-      L[1] = fmaf(-D[11], m, L[1]);
-      L[2] = fmaf(-D[13], m, L[2]);
-      L[3] = fmaf(-D[14], m, L[3]);
-      L[4] = fmaf(D[21], m, L[4]);
-      L[5] = fmaf(D[23], m, L[5]);
-      L[6] = fmaf(D[24], m, L[6]);
-      L[7] = fmaf(D[26], m, L[7]);
-      L[8] = fmaf(D[27], m, L[8]);
-      L[9] = fmaf(D[28], m, L[9]);
-      L[10] = fmaf(-D[36], m, L[10]);
-      L[11] = fmaf(-D[38], m, L[11]);
-      L[12] = fmaf(-D[39], m, L[12]);
-      L[13] = fmaf(-D[41], m, L[13]);
-      L[14] = fmaf(-D[42], m, L[14]);
-      L[15] = fmaf(-D[43], m, L[15]);
-      L[16] = fmaf(-D[45], m, L[16]);
-      L[17] = fmaf(-D[46], m, L[17]);
-      L[18] = fmaf(-D[47], m, L[18]);
-      L[19] = fmaf(-D[48], m, L[19]);
-      L[20] = fmaf(D[57], m, L[20]);
-      L[21] = fmaf(D[59], m, L[21]);
-      L[22] = fmaf(D[60], m, L[22]);
-      L[23] = fmaf(D[62], m, L[23]);
-      L[24] = fmaf(D[63], m, L[24]);
-      L[25] = fmaf(D[64], m, L[25]);
-      L[26] = fmaf(D[66], m, L[26]);
-      L[27] = fmaf(D[67], m, L[27]);
-      L[28] = fmaf(D[68], m, L[28]);
-      L[29] = fmaf(D[69], m, L[29]);
-      L[30] = fmaf(D[71], m, L[30]);
-      L[31] = fmaf(D[72], m, L[31]);
-      L[32] = fmaf(D[73], m, L[32]);
-      L[33] = fmaf(D[74], m, L[33]);
-      L[34] = fmaf(D[75], m, L[34]);
-    }
-    { const float m = __ldg(Ms + 6);
-      L[0] = fmaf(D[6], m, L[0]);
-      L[1] = fmaf(-D[12], m, L[1]);
-      L[2] = fmaf(-D[14], m, L[2]);
-      L[3] = fmaf(-D[15], m, L[3]);
-      L[4] = fmaf(D[22], m, L[4]);
-      L[5] = fmaf(D[24], m, L[5]);
-      L[6] = fmaf(D[25], m, L[6]);
-      L[7] = fmaf(D[27], m, L[7]);
-      L[8] = fmaf(D[28], m, L[8]);
-      L[9] = fmaf(D[29], m, L[9]);
-      L[10] = fmaf(-D[37], m, L[10]);
-      L[11] = fmaf(-D[39], m, L[11]);
-      L[12] = fmaf(-D[40], m, L[12]);
-      L[13] = fmaf(-D[42], m, L[13]);
-      L[14] = fmaf(-D[43], m, L[14]);
-      L[15] = fmaf(-D[44], m, L[15]);
-      L[16] = fmaf(-D[46], m, L[16]);
-      L[17] = fmaf(-D[47], m, L[17]);
-      L[18] = fmaf(-D[48], m, L[18]);
-      L[19] = fmaf(-D[49], m, L[19]);
-      L[20] = fmaf(D[58], m, L[20]);
-      L[21] = fmaf(D[60], m, L[21]);
-      L[22] = fmaf(D[61], m, L[22]);
-      L[23] = fmaf(D[63], m, L[23]);
-      L[24] = fmaf(D[64], m, L[24]);
-      L[25] = fmaf(D[65], m, L[25]);
-      L[26] = fmaf(D[67], m, L[26]);
-      L[27] = fmaf(D[68], m, L[27]);
-      L[28] = fmaf(D[69], m, L[28]);
-      L[29] = fmaf(D[70], m, L[29]);
-      L[30] = fmaf(D[72], m, L[30]);
-      L[31] = fmaf(D[73], m, L[31]);
-      L[32] = fmaf(D[74], m, L[32]);
-      L[33] = fmaf(D[75], m, L[33]);
-      L[34] = fmaf(D[76], m, L[34]);
-    }
-    { const float m = __ldg(Ms + 7);
-      L[0] = fmaf(D[7], m, L[0]);
-      L[1] = fmaf(-D[13], m, L[1]);
-      L[2] = fmaf(-D[16], m, L[2]);
-      L[3] = fmaf(-D[17], m, L[3]);
-      L[4] = fmaf(D[23], m, L[4]);
-      L[5] = fmaf(D[26], m, L[5]);
-      L[6] = fmaf(D[27], m, L[6]);
-      L[7] = fmaf(D[30], m, L[7]);
-      L[8] = fmaf(D[31], m, L[8]);
-      L[9] = fmaf(D[32], m, L[9]);
-      L[10] = fmaf(-D[38], m, L[10]);
-      L[11] = fmaf(-D[41], m, L[11]);
-      L[12] = fmaf(-D[42], m, L[12]);
-      L[13] = fmaf(-D[45], m, L[13]);
-      L[14] = fmaf(-D[46], m, L[14]);
-      L[15] = fmaf(-D[47], m, L[15]);
-      L[16] = fmaf(-D[50], m, L[16]);
-      L[17] = fmaf(-D[51], m, L[17]);
-      L[18] = fmaf(-D[52], m, L[18]);
-      L[19] = fmaf(-D[53], m, L[19]);
-      L[20] = fmaf(D[59], m, L[20]);
-      L[21] = fmaf(D[62], m, L[21]);
-      L[22] = fmaf(D[63], m, L[22]);
-      L[23] = fmaf(D[66], m, L[23]);
-      L[24] = fmaf(D[67], m, L[24]);
-      L[25] = fmaf(D[68], m, L[25]);
-      L[26] = fmaf(D[71], m, L[26]);
-      L[27] = fmaf(D[72], m, L[27]);
-      L[28] = fmaf(D[73], m, L[28]);
-      L[29] = fmaf(D[74], m, L[29]);
-      L[30] = fmaf(D[77], m, L[30]);
-      L[31] = fmaf(D[78], m, L[31]);
-      L[32] = fmaf(D[79], m, L[32]);
-      L[33] = fmaf(D[80], m, L[33]);
-      L[34] = fmaf(D[81], m, L[34]);
-    }
-    { const float m = __ldg(Ms + 8);
-      L[0] = fmaf(D[8], m, L[0]);
-      L[1] = fmaf(-D[14], m, L[1]);
-      L[2] = fmaf(-D[17], m, L[2]);
-      L[3] = fmaf(-D[18], m, L[3]);
-      L[4] = fmaf(D[24], m, L[4]);
-      L[5] = fmaf(D[27], m, L[5]);
-      L[6] = fmaf(D[28], m, L[6]);
-      L[7] = fmaf(D[31], m, L[7]);
-      L[8] = fmaf(D[32], m, L[8]);
-      L[9] = fmaf(D[33], m, L[9]);
-      L[10] = fmaf(-D[39], m, L[10]);
-      L[11] = fmaf(-D[42], m, L[11]);
-      L[12] = fmaf(-D[43], m, L[12]);
-      L[13] = fmaf(-D[46], m, L[13]);
-      L[14] = fmaf(-D[47], m, L[14]);
-      L[15] = fmaf(-D[48], m, L[15]);
-      L[16] = fmaf(-D[51], m, L[16]);
-      L[17] = fmaf(-D[52], m, L[17]);
-      L[18] = fmaf(-D[53], m, L[18]);
-      L[19] = fmaf(-D[54], m, L[19]);
-      L[20] = fmaf(D[60], m, L[20]);
-      L[21] = fmaf(D[63], m, L[21]);
-      L[22] = fmaf(D[64], m, L[22]);
-      L[23] = fmaf(D[67], m, L[23]);
-      L[24] = fmaf(D[68], m, L[24]);
-      L[25] = fmaf(D[69], m, L[25]);
-      L[26] = fmaf(D[72], m, L[26]);
-      L[27] = fmaf(D[73], m, L[27]);
-      L[28] = fmaf(D[74], m, L[28]);
-      L[29] = fmaf(D[75], m, L[29]);
-      L[30] = fmaf(D[78], m, L[30]);
-      L[31] = fmaf(D[79], m, L[31]);
-      L[32] = fmaf(D[80], m, L[32]);
-      L[33] = fmaf(D[81], m, L[33]);
-      L[34] = fmaf(D[82], m, L[34]);
-    }
-    { const float m = __ldg(Ms + 9);
-      L[0] = fmaf(D[9], m, L[0]);
-      L[1] = fmaf(-D[15], m, L[1]);
-      L[2] = fmaf(-D[18], m, L[2]);
-      L[3] = fmaf(-D[19], m, L[3]);
-      L[4] = fmaf(D[25], m, L[4]);
-      L[5] = fmaf(D[28], m, L[5]);
-      L[6] = fmaf(D[29], m, L[6]);
-      L[7] = fmaf(D[32], m, L[7]);
-      L[8] = fmaf(D[33], m, L[8]);
-      L[9] = fmaf(D[34], m, L[9]);
-      L[10] = fmaf(-D[40], m, L[10]);
-      L[11] = fmaf(-D[43], m, L[11]);
-      L[12] = fmaf(-D[44], m, L[12]);
-      L[13] = fmaf(-D[47], m, L[13]);
-      L[14] = fmaf(-D[48], m, L[14]);
-      L[15] = fmaf(-D[49], m, L[15]);
-      L[16] = fmaf(-D[52], m, L[16]);
-      L[17] = fmaf(-D[53], m, L[17]);
-      L[18] = fmaf(-D[54], m, L[18]);
-      L[19] = fmaf(-D[55], m, L[19]);
-      L[20] = fmaf(D[61], m, L[20]);
-      L[21] = fmaf(D[64], m, L[21]);
-      L[22] = fmaf(D[65], m, L[22]);
-      L[23] = fmaf(D[68], m, L[23]);
-      L[24] = fmaf(D[69], m, L[24]);
-      L[25] = fmaf(D[70], m, L[25]);
-      L[26] = fmaf(D[73], m, L[26]);
-      L[27] = fmaf(D[74], m, L[27]);
-      L[28] = fmaf(D[75], m, L[28]);
-      L[29] = fmaf(D[76], m, L[29]);
-      L[30] = fmaf(D[79], m, L[30]);
-      L[31] = fmaf(D[80], m, L[31]);
-      L[32] = fmaf(D[81], m, L[32]);
-      L[33] = fmaf(D[82], m, L[33]);
-      L[34] = fmaf(D[83], m, L[34]);
-    }
-    { const float m = __ldg(Ms + 10);
-      L[0] = fmaf(D[10], m, L[0]);
-      L[1] = fmaf(-D[20], m, L[1]);
-      L[2] = fmaf(-D[21], m, L[2]);
-      L[3] = fmaf(-D[22], m, L[3]);
-      L[4] = fmaf(D[35], m, L[4]);
-      L[5] = fmaf(D[36], m, L[5]);
-      L[6] = fmaf(D[37], m, L[6]);
-      L[7] = fmaf(D[38], m, L[7]);
-      L[8] = fmaf(D[39], m, L[8]);
-      L[9] = fmaf(D[40], m, L[9]);
-      L[10] = fmaf(-D[56], m, L[10]);
-      L[11] = fmaf(-D[57], m, L[11]);
-      L[12] = fmaf(-D[58], m, L[12]);
-      L[13] = fmaf(-D[59], m, L[13]);
-      L[14] = fmaf(-D[60], m, L[14]);
-      L[15] = fmaf(-D[61], m, L[15]);
-      L[16] = fmaf(-D[62], m, L[16]);
-      L[17] = fmaf(-D[63], m, L[17]);
-      L[18] = fmaf(-D[64], m, L[18]);
-      L[19] = fmaf(-D[65], m, L[19]);
-    }
-    { const float m = __ldg(Ms + 11);
-      L[0] = fmaf(D[11], m, L[0]);
-      L[1] = fmaf(-D[21], m, L[1]);
-      L[2] = fmaf(-D[23], m, L[2]);
-      L[3] = fmaf(-D[24], m, L[3]);
-      L[4] = fmaf(D[36], m, L[4]);
-      L[5] = fmaf(D[38], m, L[5]);
-      L[6] = fmaf(D[39], m, L[6]);
-      L[7] = fmaf(D[41], m, L[7]);
-      L[8] = fmaf(D[42], m, L[8]);
-      L[9] = fmaf(D[43], m, L[9]);
-      L[10] = fmaf(-D[57], m, L[10]);
-      L[11] = fmaf(-D[59], m, L[11]);
-      L[12] = fmaf(-D[60], m, L[12]);
-      L[13] = fmaf(-D[62], m, L[13]);
-      L[14] = fmaf(-D[63], m, L[14]);
-      L[15] = fmaf(-D[64], m, L[15]);
-      L[16] = fmaf(-D[66], m, L[16]);
-      L[17] = fmaf(-D[67], m, L[17]);
-      L[18] = fmaf(-D[68], m, L[18]);
-      L[19] = fmaf(-D[69], m, L[19]);
-    }
-    { const float m = __ldg(Ms + 12);
-      L[0] = fmaf(D[12], m, L[0]);
-      L[1] = fmaf(-D[22], m, L[1]);
-      L[2] = fmaf(-D[24], m, L[2]);
-      L[3] = fmaf(-D[25], m, L[3]);
-      L[4] = fmaf(D[37], m, L[4]);
-      L[5] = fmaf(D[39], m, L[5]);
-      L[6] = fmaf(D[40], m, L[6]);
-      L[7] = fmaf(D[42], m, L[7]);
-      L[8] = fmaf(D[43], m, L[8]);
-      L[9] = fmaf(D[44], m, L[9]);
-      L[10] = fmaf(-D[58], m, L[10]);
-      L[11] = fmaf(-D[60], m, L[11]);
-      L[12] = fmaf(-D[61], m, L[12]);
-      L[13] = fmaf(-D[63], m, L[13]);
-      L[14] = fmaf(-D[64], m, L[14]);
-      L[15] = fmaf(-D[65], m, L[15]);
-      L[16] = fmaf(-D[67], m, L[16]);
-      L[17] = fmaf(-D[68], m, L[17]);
-      L[18] = fmaf(-D[69], m, L[18]);
-      L[19] = fmaf(-D[70], m, L[19]);
-    }
-    { const float m = __ldg(Ms + 13);
-      L[0] = fmaf(D[13], m, L[0]);
-      L[1] = fmaf(-D[23], m, L[1]);
-      L[2] = fmaf(-D[26], m, L[2]);
-      L[3] = fmaf(-D[27], m, L[3]);
-      L[4] = fmaf(D[38], m, L[4]);
-      L[5] = fmaf(D[41], m, L[5]);
-      L[6] = fmaf(D[42], m, L[6]);
-      L[7] = fmaf(D[45], m, L[7]);
-      L[8] = fmaf(D[46], m, L[8]);
-      L[9] = fmaf(D[47], m, L[9]);
-      L[10] = fmaf(-D[59], m, L[10]);
-      L[11] = fmaf(-D[62], m, L[11]);
-      L[12] = fmaf(-D[63], m, L[12]);
-      L[13] = fmaf(-D[66], m, L[13]);
-      L[14] = fmaf(-D[67], m, L[14]);
-      L[15] = fmaf(-D[68], m, L[15]);
-      L[16] = fmaf(-D[71], m, L[16]);
-      L[17] = fmaf(-D[72], m, L[17]);
-      L[18] = fmaf(-D[73], m, L[18]);
-      L[19] = fmaf(-D[74], m, L[19]);
-    }
-    { const float m = __ldg(Ms + 14);
-      L[0] = fmaf(D[14], m, L[0]);
-      L[1] = fmaf(-D[24], m, L[1]);
-      L[2] = fmaf(-D[27], m, L[2]);
-      L[3] = fmaf(-D[28], m, L[3]);
-      L[4] = fmaf(D[39], m, L[4]);
-      L[5] = fmaf(D[42], m, L[5]);
-      L[6] = fmaf(D[43], m, L[6]);
-      L[7] = fmaf(D[46], m, L[7]);
-      L[8] = fmaf(D[47], m, L[8]);
-      L[9] = fmaf(D[48], m, L[9]);
-      L[10] = fmaf(-D[60], m, L[10]);
-      L[11] = fmaf(-D[63], m, L[11]);
-      L[12] = fmaf(-D[64], m, L[12]);
-      L[13] = fmaf(-D[67], m, L[13]);
-      L[14] = fmaf(-D[68], m, L[14]);
-      L[15] = fmaf(-D[69], m, L[15]);
-      L[16] = fmaf(-D[72], m, L[16]);
-      L[17] = fmaf(-D[73], m, L[17]);
-      L[18] = fmaf(-D[74], m, L[18]);
-      L[19] = fmaf(-D[75], m, L[19]);
-    }
-    { const float m = __ldg(Ms + 15);
-      L[0] = fmaf(D[15], m, L[0]);
-      L[1] = fmaf(-D[25], m, L[1]);
-      L[2] = fmaf(-D[28], m, L[2]);
-      L[3] = fmaf(-D[29], m, L[3]);
-      L[4] = fmaf(D[40], m, L[4]);
-      L[5] = fmaf(D[43], m, L[5]);
-      L[6] = fmaf(D[44], m, L[6]);
-      L[7] = fmaf(D[47], m, L[7]);
-      L[8] = fmaf(D[48], m, L[8]);
-      L[9] = fmaf(D[49], m, L[9]);
-      L[10] = fmaf(-D[61], m, L[10]);
-      L[11] = fmaf(-D[64], m, L[11]);
-      L[12] = fmaf(-D[65], m, L[12]);
-      L[13] = fmaf(-D[68], m, L[13]);
-      L[14] = fmaf(-D[69], m, L[14]);
-      L[15] = fmaf(-D[70], m, L[15]);
-      L[16] = fmaf(-D[73], m, L[16]);
-      L[17] = fmaf(-D[74], m, L[17]);
-      L[18] = fmaf(-D[75], m, L[18]);
-      L[19] = fmaf(-D[76], m, L[19]);
-    }
-    { const float m = __ldg(Ms + 16);
-      L[0] = fmaf(D[16], m, L[0]);
-      L[1] = fmaf(-D[26], m, L[1]);
-      L[2] = fmaf(-D[30], m, L[2]);
-      L[3] = fmaf(-D[31], m, L[3]);
-      L[4] = fmaf(D[41], m, L[4]);
-      L[5] = fmaf(D[45], m, L[5]);
-      L[6] = fmaf(D[46], m, L[6]);
-      L[7] = fmaf(D[50], m, L[7]);
-      L[8] = fmaf(D[51], m, L[8]);
-      L[9] = fmaf(D[52], m, L[9]);
-      L[10] = fmaf(-D[62], m, L[10]);
-      L[11] = fmaf(-D[66], m, L[11]);
-      L[12] = fmaf(-D[67], m, L[12]);
-      L[13] = fmaf(-D[71], m, L[13]);
-      L[14] = fmaf(-D[72], m, L[14]);
-      L[15] = fmaf(-D[73], m, L[15]);
-      L[16] = fmaf(-D[77], m, L[16]);
-      L[17] = fmaf(-D[78], m, L[17]);
-      L[18] = fmaf(-D[79], m, L[18]);
-      L[19] = fmaf(-D[80], m, L[19]);
-    }
-    { const float m = __ldg(Ms + 17);
-      L[0] = fmaf(D[17], m, L[0]);
-      L[1] = fmaf(-D[27], m, L[1]);
-      L[2] = fmaf(-D[31], m, L[2]);
-      L[3] = fmaf(-D[32], m, L[3]);
-      L[4] = fmaf(D[42], m, L[4]);
-      L[5] = fmaf(D[46], m, L[5]);
-      L[6] = fmaf(D[47], m, L[6]);
-      L[7] = fmaf(D[51], m, L[7]);
-      L[8] = fmaf(D[52], m, L[8]);
-      L[9] = fmaf(D[53], m, L[9]);
-      L[10] = fmaf(-D[63], m, L[10]);
-      L[11] = fmaf(-D[67], m, L[11]);
-      L[12] = fmaf(-D[68], m, L[12]);
-      L[13] = fmaf(-D[72], m, L[13]);
-      L[14] = fmaf(-D[73], m, L[14]);
-      L[15] = fmaf(-D[74], m, L[15]);
-      L[16] = fmaf(-D[78], m, L[16]);
-      L[17] = fmaf(-D[79], m, L[17]);
-      L[18] = fmaf(-D[80], m, L[18]);
-      L[19] = fmaf(-D[81], m, L[19]);
-    }
-    { const float m = __ldg(Ms + 18);
-      L[0] = fmaf(D[18], m, L[0]);
-      L[1] = fmaf(-D[28], m, L[1]);
-      L[2] = fmaf(-D[32], m, L[2]);
-      L[3] = fmaf(-D[33], m, L[3]);
-      L[4] = fmaf(D[43], m, L[4]);
-      L[5] = fmaf(D[47], m, L[5]);
-      L[6] = fmaf(D[48], m, L[6]);
-      L[7] = fmaf(D[52], m, L[7]);
-      L[8] = fmaf(D[53], m, L[8]);
-      L[9] = fmaf(D[54], m, L[9]);
-      L[10] = fmaf(-D[64], m, L[10]);
-      L[11] = fmaf(-D[68], m, L[11]);
-      L[12] = fmaf(-D[69], m, L[12]);
-      L[13] = fmaf(-D[73], m, L[13]);
-      L[14] = fmaf(-D[74], m, L[14]);
-      L[15] = fmaf(-D[75], m, L[15]);
-      L[16] = fmaf(-D[79], m, L[16]);
-      L[17] = fmaf(-D[80], m, L[17]);
-      L[18] = fmaf(-D[81], m, L[18]);
-      L[19] = fmaf(-D[82], m, L[19]);
-    }
-    { const float m = __ldg(Ms + 19);
-      L[0] = fmaf(D[19], m, L[0]);
-      L[1] = fmaf(-D[29], m, L[1]);
-      L[2] = fmaf(-D[33], m, L[2]);
-      L[3] = fmaf(-D[34], m, L[3]);
-      L[4] = fmaf(D[44], m, L[4]);
-      L[5] = fmaf(D[48], m, L[5]);
-      L[6] = fmaf(D[49], m, L[6]);
-      L[7] = fmaf(D[53], m, L[7]);
-      L[8] = fmaf(D[54], m, L[8]);
-      L[9] = fmaf(D[55], m, L[9]);
-      L[10] = fmaf(-D[65], m, L[10]);
-      L[11] = fmaf(-D[69], m, L[11]);
-      L[12] = fmaf(-D[70], m, L[12]);
-      L[13] = fmaf(-D[74], m, L[13]);
-      L[14] = fmaf(-D[75], m, L[14]);
-      L[15] = fmaf(-D[76], m, L[15]);
-      L[16] = fmaf(-D[80], m, L[16]);
-      L[17] = fmaf(-D[81], m, L[17]);
-      L[18] = fmaf(-D[82], m, L[18]);
-      L[19] = fmaf(-D[83], m, L[19]);
-    }
-    { const float m = __ldg(Ms + 20);
-      L[0] = fmaf(D[20], m, L[0]);
-      L[1] = fmaf(-D[35], m, L[1]);
-      L[2] = fmaf(-D[36], m, L[2]);
-      L[3] = fmaf(-D[37], m, L[3]);
-      L[4] = fmaf(D[56], m, L[4]);
-      L[5] = fmaf(D[57], m, L[5]);
-      L[6] = fmaf(D[58], m, L[6]);
-      L[7] = fmaf(D[59], m, L[7]);
-      L[8] = fmaf(D[60], m, L[8]);
-      L[9] = fmaf(D[61], m, L[9]);
-    }
-    { const float m = __ldg(Ms + 21);
-      L[0] = fmaf(D[21], m, L[0]);
-      L[1] = fmaf(-D[36], m, L[1]);
-      L[2] = fmaf(-D[38], m, L[2]);
-      L[3] = fmaf(-D[39], m, L[3]);
-      L[4] = fmaf(D[57], m, L[4]);
-      L[5] = fmaf(D[59], m, L[5]);
-      L[6] = fmaf(D[60], m, L[6]);
-      L[7] = fmaf(D[62], m, L[7]);
-      L[8] = fmaf(D[63], m, L[8]);
-      L[9] = fmaf(D[64], m, L[9]);
-    }
-    { const float m = __ldg(Ms + 22);
-      L[0] = fmaf(D[22], m, L[0]);
-      L[1] = fmaf(-D[37], m, L[1]);
-      L[2] = fmaf(-D[39], m, L[2]);
-      L[3] = fmaf(-D[40], m, L[3]);
-      L[4] = fmaf(D[58], m, L[4]);
-      L[5] = fmaf(D[60], m, L[5]);
-      L[6] = fmaf(D[61], m, L[6]);
-      L[7] = fmaf(D[63], m, L[7]);
-      L[8] = fmaf(D[64], m, L[8]);
-      L[9] = fmaf(D[65], m, L[9]);
-    }
-    { const float m = __ldg(Ms + 23);
-      L[0] = fmaf(D[23], m, L[0]);
-      L[1] = fmaf(-D[38], m, L[1]);
-      L[2] = fmaf(-D[41], m, L[2]);
-      L[3] = fmaf(-D[42], m, L[3]);
-      L[4] = fmaf(D[59], m, L[4]);
-      L[5] = fmaf(D[62], m, L[5]);
-      L[6] = fmaf(D[63], m, L[6]);
-      L[7] = fmaf(D[66], m, L[7]);
-      L[8] = fmaf(D[67], m, L[8]);
-      L[9] = fmaf(D[68], m, L[9]);
-    }
-    { const float m = __ldg(Ms + 24);
-      L[0] = fmaf(D[24], m, L[0]);
-      L[1] = fmaf(-D[39], m, L[1]);
-      L[2] = fmaf(-D[42], m, L[2]);
-      L[3] = fmaf(-D[43], m, L[3]);
-      L[4] = fmaf(D[60], m, L[4]);
-      L[5] = fmaf(D[63], m, L[5]);
-      L[6] = fmaf(D[64], m, L[6]);
-      L[7] = fmaf(D[67], m, L[7]);
-      L[8] = fmaf(D[68], m, L[8]);
-      L[9] = fmaf(D[69], m, L[9]);
-    }
-    { const float m = __ldg(Ms + 25);
-      L[0] = fmaf(D[25], m, L[0]);
-      L[1] = fmaf(-D[40], m, L[1]);
-      L[2] = fmaf(-D[43], m, L[2]);
-      L[3] = fmaf(-D[44], m, L[3]);
-      L[4] = fmaf(D[61], m, L[4]);
-      L[5] = fmaf(D[64], m, L[5]);
-      L[6] = fmaf(D[65], m, L[6]);
-      L[7] = fmaf(D[68], m, L[7]);
-      L[8] = fmaf(D[69], m, L[8]);
-      L[9] = fmaf(D[70], m, L[9]);
-    }
-    { const float m = __ldg(Ms + 26);
-      L[0] = fmaf(D[26], m, L[0]);
-      L[1] = fmaf(-D[41], m, L[1]);
-      L[2] = fmaf(-D[45], m, L[2]);
-      L[3] = fmaf(-D[46], m, L[3]);
-      L[4] = fmaf(D[62], m, L[4]);
-      L[5] = fmaf(D[66], m, L[5]);
-      L[6] = fmaf(D[67], m, L[6]);
-      L[7] = fmaf(D[71], m, L[7]);
-      L[8] = fmaf(D[72], m, L[8]);
-      L[9] = fmaf(D[73], m, L[9]);
-    }
-    { const float m = __ldg(Ms + 27);
-      L[0] = fmaf(D[27], m, L[0]);
-      L[1] = fmaf(-D[42], m, L[1]);
-      L[2] = fmaf(-D[46], m, L[2]);
-      L[3] = fmaf(-D[47], m, L[3]);
-      L[4] = fmaf(D[63], m, L[4]);
-      L[5] = fmaf(D[67], m, L[5]);
-      L[6] = fmaf(D[68], m, L[6]);
-      L[7] = fmaf(D[72], m, L[7]);
-      L[8] = fmaf(D[73], m, L[8]);
-      L[9] = fmaf(D[74], m, L[9]);
-    }
-    { const float m = __ldg(Ms + 28);
-      L[0] = fmaf(D[28], m, L[0]);
-      L[1] = fmaf(-D[43], m, L[1]);
-      L[2] = fmaf(-D[47], m, L[2]);
-      L[3] = fmaf(-D[48], m, L[3]);
-      L[4] = fmaf(D[64], m, L[4]);
-      L[5] = fmaf(D[68], m, L[5]);
-      L[6] = fmaf(D[69], m, L[6]);
-      L[7] = fmaf(D[73], m, L[7]);
-      L[8] = fmaf(D[74], m, L[8]);
-      L[9] = fmaf(D[75], m, L[9]);
-    }
-    { const float m = __ldg(Ms + 29);
-      L[0] = fmaf(D[29], m, L[0]);
-      L[1] = fmaf(-D[44], m, L[1]);
-      L[2] = fmaf(-D[48], m, L[2]);
-      L[3] = fmaf(-D[49], m, L[3]);
-      L[4] = fmaf(D[65], m, L[4]);
-      L[5] = fmaf(D[69], m, L[5]);
-      L[6] = fmaf(D[70], m, L[6]);
-      L[7] = fmaf(D[74], m, L[7]);
-      L[8] = fmaf(D[75], m, L[8]);
-      L[9] = fmaf(D[76], m, L[9]);
-    }
-    { const float m = __ldg(Ms + 30);
-      L[0] = fmaf(D[30], m, L[0]);
-      L[1] = fmaf(-D[45], m, L[1]);
-      L[2] = fmaf(-D[50], m, L[2]);
-      L[3] = fmaf(-D[51], m, L[3]);
-      L[4] = fmaf(D[66], m, L[4]);
-      L[5] = fmaf(D[71], m, L[5]);
-      L[6] = fmaf(D[72], m, L[6]);
-      L[7] = fmaf(D[77], m, L[7]);
-      L[8] = fmaf(D[78], m, L[8]);
-      L[9] = fmaf(D[79], m, L[9]);
-    }
-    { const float m = __ldg(Ms + 31);
-      L[0] = fmaf(D[31], m, L[0]);
-      L[1] = fmaf(-D[46], m, L[1]);
-      L[2] = fmaf(-D[51], m, L[2]);
-      L[3] = fmaf(-D[52], m, L[3]);
-      L[4] = fmaf(D[67], m, L[4]);
-      L[5] = fmaf(D[72], m, L[5]);
-      L[6] = fmaf(D[73], m, L[6]);
-      L[7] = fmaf(D[78], m, L[7]);
-      L[8] = fmaf(D[79], m, L[8]);
-      L[9] = fmaf(D[80], m, L[9]);
-    }
-    { const float m = __ldg(Ms + 32);
-      L[0] = fmaf(D[32], m, L[0]);
-      L[1] = fmaf(-D[47], m, L[1]);
-      L[2] = fmaf(-D[52], m, L[2]);
-      L[3] = fmaf(-D[53], m, L[3]);
-      L[4] = fmaf(D[68], m, L[4]);
-      L[5] = fmaf(D[73], m, L[5]);
-      L[6] = fmaf(D[74], m, L[6]);
-      L[7] = fmaf(D[79], m, L[7]);
-      L[8] = fmaf(D[80], m, L[8]);
-      L[9] = fmaf(D[81], m, L[9]);
-    }
-    { const float m = __ldg(Ms + 33);
-      L[0] = fmaf(D[33], m, L[0]);
-      L[1] = fmaf(-D[48], m, L[1]);
-      L[2] = fmaf(-D[53], m, L[2]);
-      L[3] = fmaf(-D[54], m, L[3]);
-      L[4] = fmaf(D[69], m, L[4]);
-      L[5] = fmaf(D[74], m, L[5]);
-      L[6] = fmaf(D[75], m, L[6]);
-      L[7] = fmaf(D[80], m, L[7]);
-      L[8] = fmaf(D[81], m, L[8]);
-      L[9] = fmaf(D[82], m, L[9]);
-    }
-    { const float m = __ldg(Ms + 34);
-      L[0] = fmaf(D[34], m, L[0]);
-      L[1] = fmaf(-D[49], m, L[1]);
-      L[2] = fmaf(-D[54], m, L[2]);
-      L[3] = fmaf(-D[55], m, L[3]);
-      L[4] = fmaf(D[70], m, L[4]);
-      L[5] = fmaf(D[75], m, L[5]);
-      L[6] = fmaf(D[76], m, L[6]);
-      L[7] = fmaf(D[81], m, L[7]);
-      L[8] = fmaf(D[82], m, L[8]);
-      L[9] = fmaf(D[83], m, L[9]);
-    }
-    { const float m = __ldg(Ms + 35);
-      L[0] = fmaf(D[35], m, L[0]);
-      L[1] = fmaf(-D[56], m, L[1]);
-      L[2] = fmaf(-D[57], m, L[2]);
-      L[3] = fmaf(-D[58], m, L[3]);
-    }
-    { const float m = __ldg(Ms + 36);
-      L[0] = fmaf(D[36], m, L[0]);
-      L[1] = fmaf(-D[57], m, L[1]);
-      L[2] = fmaf(-D[59], m, L[2]);
-      L[3] = fmaf(-D[60], m, L[3]);
-    }
-    { const float m = __ldg(Ms + 37);
-      L[0] = fmaf(D[37], m, L[0]);
-      L[1] = fmaf(-D[58], m, L[1]);
-      L[2] = fmaf(-D[60], m, L[2]);
-      L[3] = fmaf(-D[61], m, L[3]);
-    }
-    { const float m = __ldg(Ms + 38);
-      L[0] = fmaf(D[38], m, L[0]);
-      L[1] = fmaf(-D[59], m, L[1]);
-      L[2] = fmaf(-D[62], m, L[2]);
-      L[3] = fmaf(-D[63], m, L[3]);
-    }
-    { const float m = __ldg(Ms + 39);
-      L[0] = fmaf(D[39], m, L[0]);
-      L[1] = fmaf(-D[60], m, L[1]);
-      L[2] = fmaf(-D[63], m, L[2]);
-      L[3] = fmaf(-D[64], m, L[3]);
-    }
-    { const float m = __ldg(Ms + 40);
-      L[0] = fmaf(D[40], m, L[0]);
-      L[1] = fmaf(-D[61], m, L[1]);
-      L[2] = fmaf(-D[64], m, L[2]);
-      L[3] = fmaf(-D[65], m, L[3]);
-    }
-    { const float m = __ldg(Ms + 41);
-      L[0] = fmaf(D[41], m, L[0]);
-      L[1] = fmaf(-D[62], m, L[1]);
-      L[2] = fmaf(-D[66], m, L[2]);
-      L[3] = fmaf(-D[67], m, L[3]);
-    }
-    { const float m = __ldg(Ms + 42);
-      L[0] = fmaf(D[42], m, L[0]);
-      L[1] = fmaf(-D[63], m, L[1]);
-      L[2] = fmaf(-D[67], m, L[2]);
-      L[3] = fmaf(-D[68], m, L[3]);
-    }
-    { const float m = __ldg(Ms + 43);
-      L[0] = fmaf(D[43], m, L[0]);
-      L[1] = fmaf(-D[64], m, L[1]);
-      L[2] = fmaf(-D[68], m, L[2]);
-      L[3] = fmaf(-D[69], m, L[3]);
-    }
-    { const float m = __ldg(Ms + 44);
-      L[0] = fmaf(D[44], m, L[0]);
-      L[1] = fmaf(-D[65], m, L[1]);
-      L[2] = fmaf(-D[69], m, L[2]);
-      L[3] = fmaf(-D[70], m, L[3]);
-    }
-    { const float m = __ldg(Ms + 45);
-      L[0] = fmaf(D[45], m, L[0]);
-      L[1] = fmaf(-D[66], m, L[1]);
-      L[2] = fmaf(-D[71], m, L[2]);
-      L[3] = fmaf(-D[72], m, L[3]);
-    }
-    { const float m = __ldg(Ms + 46);
-      L[0] = fmaf(D[46], m, L[0]);
-      L[1] = fmaf(-D[67], m, L[1]);
-      L[2] = fmaf(-D[72], m, L[2]);
-      L[3] = fmaf(-D[73], m, L[3]);
-    }
-    { const float m = __ldg(Ms + 47);
-      L[0] = fmaf(D[47], m, L[0]);
-      L[1] = fmaf(-D[68], m, L[1]);
-      L[2] = fmaf(-D[73], m, L[2]);
-      L[3] = fmaf(-D[74], m, L[3]);
-    }
-    { const float m = __ldg(Ms + 48);
-      L[0] = fmaf(D[48], m, L[0]);
-      L[1] = fmaf(-D[69], m, L[1]);
-      L[2] = fmaf(-D[74], m, L[2]);
-      L[3] = fmaf(-D[75], m, L[3]);
-    }
-    { const float m = __ldg(Ms + 49);
-      L[0] = fmaf(D[49], m, L[0]);
-      L[1] = fmaf(-D[70], m, L[1]);
-      L[2] = fmaf(-D[75], m, L[2]);
-      L[3] = fmaf(-D[76], m, L[3]);
-    }
-    { const float m = __ldg(Ms + 50);
-      L[0] = fmaf(D[50], m, L[0]);
-      L[1] = fmaf(-D[71], m, L[1]);
-      L[2] = fmaf(-D[77], m, L[2]);
-      L[3] = fmaf(-D[78], m, L[3]);
-    }
-    { const float m = __ldg(Ms + 51);
-      L[0] = fmaf(D[51], m, L[0]);
-      L[1] = fmaf(-D[72], m, L[1]);
-      L[2] = fmaf(-D[78], m, L[2]);
-      L[3] = fmaf(-D[79], m, L[3]);
-    }
-    { const float m = __ldg(Ms + 52);
-      L[0] = fmaf(D[52], m, L[0]);
-      L[1] = fmaf(-D[73], m, L[1]);
-      L[2] = fmaf(-D[79], m, L[2]);
-      L[3] = fmaf(-D[80], m, L[3]);
-    }
-    { const float m = __ldg(Ms + 53);
-      L[0] = fmaf(D[53], m, L[0]);
-      L[1] = fmaf(-D[74], m, L[1]);
-      L[2] = fmaf(-D[80], m, L[2]);
-      L[3] = fmaf(-D[81], m, L[3]);
-    }
-    { const float m = __ldg(Ms + 54);
-      L[0] = fmaf(D[54], m, L[0]);
-      L[1] = fmaf(-D[75], m, L[1]);
-      L[2] = fmaf(-D[81], m, L[2]);
-      L[3] = fmaf(-D[82], m, L[3]);
-    }
-    { const float m = __ldg(Ms + 55);
-      L[0] = fmaf(D[55], m, L[0]);
-      L[1] = fmaf(-D[76], m, L[1]);
-      L[2] = fmaf(-D[82], m, L[2]);
-      L[3] = fmaf(-D[83], m, L[3]);
-    }
-    { const float m = __ldg(Ms + 56);
-      L[0] = fmaf(D[56], m, L[0]);
-    }
-    { const float m = __ldg(Ms + 57);
-      L[0] = fmaf(D[57], m, L[0]);
-    }
-    { const float m = __ldg(Ms + 58);
-      L[0] = fmaf(D[58], m, L[0]);
-    }
-    { const float m = __ldg(Ms + 59);
-      L[0] = fmaf(D[59], m, L[0]);
-    }
-    { const float m = __ldg(Ms + 60);
-      L[0] = fmaf(D[60], m, L[0]);
-    }
-    { const float m = __ldg(Ms + 61);
-      L[0] = fmaf(D[61], m, L[0]);
-    }
-    { const float m = __ldg(Ms + 62);
-      L[0] = fmaf(D[62], m, L[0]);
-    }
-    { const float m = __ldg(Ms + 63);
-      L[0] = fmaf(D[63], m, L[0]);
-    }
-    { const float m = __ldg(Ms + 64);
-      L[0] = fmaf(D[64], m, L[0]);
-    }
-    { const float m = __ldg(Ms + 65);
-      L[0] = fmaf(D[65], m, L[0]);
-    }
-    { const float m = __ldg(Ms + 66);
-      L[0] = fmaf(D[66], m, L[0]);
-    }
-    { const float m = __ldg(Ms + 67);
-      L[0] = fmaf(D[67], m, L[0]);
-    }
-    { const float m = __ldg(Ms + 68);
-      L[0] = fmaf(D[68], m, L[0]);
-    }
-    { const float m = __ldg(Ms + 69);
-      L[0] = fmaf(D[69], m, L[0]);
-    }
-    { const float m = __ldg(Ms + 70);
-      L[0] = fmaf(D[70], m, L[0]);
-    }
-    { const float m = __ldg(Ms + 71);
-      L[0] = fmaf(D[71], m, L[0]);
-    }
-    { const float m = __ldg(Ms + 72);
-      L[0] = fmaf(D[72], m, L[0]);
-    }
-    { const float m = __ldg(Ms + 73);
-      L[0] = fmaf(D[73], m, L[0]);
-    }
-    { const float m = __ldg(Ms + 74);
-      L[0] = fmaf(D[74], m, L[0]);
-    }
-    { const float m = __ldg(Ms + 75);
-      L[0] = fmaf(D[75], m, L[0]);
-    }
-    { const float m = __ldg(Ms + 76);
-      L[0] = fmaf(D[76], m, L[0]);
-    }
-    { const float m = __ldg(Ms + 77);
-      L[0] = fmaf(D[77], m, L[0]);
-    }
-    { const float m = __ldg(Ms + 78);
-      L[0] = fmaf(D[78], m, L[0]);
-    }
-    { const float m = __ldg(Ms + 79);
-      L[0] = fmaf(D[79], m, L[0]);
-    }
-    { const float m = __ldg(Ms + 80);
-      L[0] = fmaf(D[80], m, L[0]);
-    }
-    { const float m = __ldg(Ms + 81);
-      L[0] = fmaf(D[81], m, L[0]);
-    }
-    { const float m = __ldg(Ms + 82);
-      L[0] = fmaf(D[82], m, L[0]);
-    }
-    { const float m = __ldg(Ms + 83);
-      L[0] = fmaf(D[83], m, L[0]);
+    { const T m = __ldg(Ms + 1);
+      L[0] = m2l_fma(D[1], m, L[0]);
+      L[1] = m2l_fma(-D[4], m, L[1]);
+      L[2] = m2l_fma(-D[5], m, L[2]);
+      L[3] = m2l_fma(-D[6], m, L[3]);
+      L[4] = m2l_fma(D[10], m, L[4]);
+      L[5] = m2l_fma(D[11], m, L[5]);
+      L[6] = m2l_fma(D[12], m, L[6]);
+      L[7] = m2l_fma(D[13], m, L[7]);
+      L[8] = m2l_fma(D[14], m, L[8]);
+      L[9] = m2l_fma(D[15], m, L[9]);
+      L[10] = m2l_fma(-D[20], m, L[10]);
+      L[11] = m2l_fma(-D[21], m, L[11]);
+      L[12] = m2l_fma(-D[22], m, L[12]);
+      L[13] = m2l_fma(-D[23], m, L[13]);
+      L[14] = m2l_fma(-D[24], m, L[14]);
+      L[15] = m2l_fma(-D[25], m, L[15]);
+      L[16] = m2l_fma(-D[26], m, L[16]);
+      L[17] = m2l_fma(-D[27], m, L[17]);
+      L[18] = m2l_fma(-D[28], m, L[18]);
+      L[19] = m2l_fma(-D[29], m, L[19]);
+      L[20] = m2l_fma(D[35], m, L[20]);
+      L[21] = m2l_fma(D[36], m, L[21]);
+      L[22] = m2l_fma(D[37], m, L[22]);
+      L[23] = m2l_fma(D[38], m, L[23]);
+      L[24] = m2l_fma(D[39], m, L[24]);
+      L[25] = m2l_fma(D[40], m, L[25]);
+      L[26] = m2l_fma(D[41], m, L[26]);
+      L[27] = m2l_fma(D[42], m, L[27]);
+      L[28] = m2l_fma(D[43], m, L[28]);
+      L[29] = m2l_fma(D[44], m, L[29]);
+      L[30] = m2l_fma(D[45], m, L[30]);
+      L[31] = m2l_fma(D[46], m, L[31]);
+      L[32] = m2l_fma(D[47], m, L[32]);
+      L[33] = m2l_fma(D[48], m, L[33]);
+      L[34] = m2l_fma(D[49], m, L[34]);
+      L[35] = m2l_fma(-D[56], m, L[35]);
+      L[36] = m2l_fma(-D[57], m, L[36]);
+      L[37] = m2l_fma(-D[58], m, L[37]);
+      L[38] = m2l_fma(-D[59], m, L[38]);
+      L[39] = m2l_fma(-D[60], m, L[39]);
+      L[40] = m2l_fma(-D[61], m, L[40]);
+      L[41] = m2l_fma(-D[62], m, L[41]);
+      L[42] = m2l_fma(-D[63], m, L[42]);
+      L[43] = m2l_fma(-D[64], m, L[43]);
+      L[44] = m2l_fma(-D[65], m, L[44]);
+      L[45] = m2l_fma(-D[66], m, L[45]);
+      L[46] = m2l_fma(-D[67], m, L[46]);
+      L[47] = m2l_fma(-D[68], m, L[47]);
+      L[48] = m2l_fma(-D[69], m, L[48]);
+      L[49] = m2l_fma(-D[70], m, L[49]);
+      L[50] = m2l_fma(-D[71], m, L[50]);
+      L[51] = m2l_fma(-D[72], m, L[51]);
+      L[52] = m2l_fma(-D[73], m, L[52]);
+      L[53] = m2l_fma(-D[74], m, L[53]);
+      L[54] = m2l_fma(-D[75], m, L[54]);
+      L[55] = m2l_fma(-D[76], m, L[55]);
+    }
+    { const T m = __ldg(Ms + 2);
+      L[0] = m2l_fma(D[2], m, L[0]);
+      L[1] = m2l_fma(-D[5], m, L[1]);
+      L[2] = m2l_fma(-D[7], m, L[2]);
+      L[3] = m2l_fma(-D[8], m, L[3]);
+      L[4] = m2l_fma(D[11], m, L[4]);
+      L[5] = m2l_fma(D[13], m, L[5]);
+      L[6] = m2l_fma(D[14], m, L[6]);
+      L[7] = m2l_fma(D[16], m, L[7]);
+      L[8] = m2l_fma(D[17], m, L[8]);
+      L[9] = m2l_fma(D[18], m, L[9]);
+      L[10] = m2l_fma(-D[21], m, L[10]);
+      L[11] = m2l_fma(-D[23], m, L[11]);
+      L[12] = m2l_fma(-D[24], m, L[12]);
+      L[13] = m2l_fma(-D[26], m, L[13]);
+      L[14] = m2l_fma(-D[27], m, L[14]);
+      L[15] = m2l_fma(-D[28], m, L[15]);
+      L[16] = m2l_fma(-D[30], m, L[16]);
+      L[17] = m2l_fma(-D[31], m, L[17]);
+      L[18] = m2l_fma(-D[32], m, L[18]);
+      L[19] = m2l_fma(-D[33], m, L[19]);
+      L[20] = m2l_fma(D[36], m, L[20]);
+      L[21] = m2l_fma(D[38], m, L[21]);
+      L[22] = m2l_fma(D[39], m, L[22]);
+      L[23] = m2l_fma(D[41], m, L[23]);
+      L[24] = m2l_fma(D[42], m, L[24]);
+      L[25] = m2l_fma(D[43], m, L[25]);
+      L[26] = m2l_fma(D[45], m, L[26]);
+      L[27] = m2l_fma(D[46], m, L[27]);
+      L[28] = m2l_fma(D[47], m, L[28]);
+      L[29] = m2l_fma(D[48], m, L[29]);
+      L[30] = m2l_fma(D[50], m, L[30]);
+      L[31] = m2l_fma(D[51], m, L[31]);
+      L[32] = m2l_fma(D[52], m, L[32]);
+      L[33] = m2l_fma(D[53], m, L[33]);
+      L[34] = m2l_fma(D[54], m, L[34]);
+      L[35] = m2l_fma(-D[57], m, L[35]);
+      L[36] = m2l_fma(-D[59], m, L[36]);
+      L[37] = m2l_fma(-D[60], m, L[37]);
+      L[38] = m2l_fma(-D[62], m, L[38]);
+      L[39] = m2l_fma(-D[63], m, L[39]);
+      L[40] = m2l_fma(-D[64], m, L[40]);
+      L[41] = m2l_fma(-D[66], m, L[41]);
+      L[42] = m2l_fma(-D[67], m, L[42]);
+      L[43] = m2l_fma(-D[68], m, L[43]);
+      L[44] = m2l_fma(-D[69], m, L[44]);
+      L[45] = m2l_fma(-D[71], m, L[45]);
+      L[46] = m2l_fma(-D[72], m, L[46]);
+      L[47] = m2l_fma(-D[73], m, L[47]);
+      L[48] = m2l_fma(-D[74], m, L[48]);
+      L[49] = m2l_fma(-D[75], m, L[49]);
+      L[50] = m2l_fma(-D[77], m, L[50]);
+      L[51] = m2l_fma(-D[78], m, L[51]);
+      L[52] = m2l_fma(-D[79], m, L[52]);
+      L[53] = m2l_fma(-D[80], m, L[53]);
+      L[54] = m2l_fma(-D[81], m, L[54]);
+      L[55] = m2l_fma(-D[82], m, L[55]);
+    }
+    { const T m = __ldg(Ms + 3);
+      L[0] = m2l_fma(D[3], m, L[0]);
+      L[1] = m2l_fma(-D[6], m, L[1]);
+      L[2] = m2l_fma(-D[8], m, L[2]);
+      L[3] = m2l_fma(-D[9], m, L[3]);
+      L[4] = m2l_fma(D[12], m, L[4]);
+      L[5] = m2l_fma(D[14], m, L[5]);
+      L[6] = m2l_fma(D[15], m, L[6]);
+      L[7] = m2l_fma(D[17], m, L[7]);
+      L[8] = m2l_fma(D[18], m, L[8]);
+      L[9] = m2l_fma(D[19], m, L[9]);
+      L[10] = m2l_fma(-D[22], m, L[10]);
+      L[11] = m2l_fma(-D[24], m, L[11]);
+      L[12] = m2l_fma(-D[25], m, L[12]);
+      L[13] = m2l_fma(-D[27], m, L[13]);
+      L[14] = m2l_fma(-D[28], m, L[14]);
+      L[15] = m2l_fma(-D[29], m, L[15]);
+      L[16] = m2l_fma(-D[31], m, L[16]);
+      L[17] = m2l_fma(-D[32], m, L[17]);
+      L[18] = m2l_fma(-D[33], m, L[18]);
+      L[19] = m2l_fma(-D[34], m, L[19]);
+      L[20] = m2l_fma(D[37], m, L[20]);
+      L[21] = m2l_fma(D[39], m, L[21]);
+      L[22] = m2l_fma(D[40], m, L[22]);
+      L[23] = m2l_fma(D[42], m, L[23]);
+      L[24] = m2l_fma(D[43], m, L[24]);
+      L[25] = m2l_fma(D[44], m, L[25]);
+      L[26] = m2l_fma(D[46], m, L[26]);
+      L[27] = m2l_fma(D[47], m, L[27]);
+      L[28] = m2l_fma(D[48], m, L[28]);
+      L[29] = m2l_fma(D[49], m, L[29]);
+      L[30] = m2l_fma(D[51], m, L[30]);
+      L[31] = m2l_fma(D[52], m, L[31]);
+      L[32] = m2l_fma(D[53], m, L[32]);
+      L[33] = m2l_fma(D[54], m, L[33]);
+      L[34] = m2l_fma(D[55], m, L[34]);
+      L[35] = m2l_fma(-D[58], m, L[35]);
+      L[36] = m2l_fma(-D[60], m, L[36]);
+      L[37] = m2l_fma(-D[61], m, L[37]);
+      L[38] = m2l_fma(-D[63], m, L[38]);
+      L[39] = m2l_fma(-D[64], m, L[39]);
+      L[40] = m2l_fma(-D[65], m, L[40]);
+      L[41] = m2l_fma(-D[67], m, L[41]);
+      L[42] = m2l_fma(-D[68], m, L[42]);
+      L[43] = m2l_fma(-D[69], m, L[43]);
+      L[44] = m2l_fma(-D[70], m, L[44]);
+      L[45] = m2l_fma(-D[72], m, L[45]);
+      L[46] = m2l_fma(-D[73], m, L[46]);
+      L[47] = m2l_fma(-D[74], m, L[47]);
+      L[48] = m2l_fma(-D[75], m, L[48]);
+      L[49] = m2l_fma(-D[76], m, L[49]);
+      L[50] = m2l_fma(-D[78], m, L[50]);
+      L[51] = m2l_fma(-D[79], m, L[51]);
+      L[52] = m2l_fma(-D[80], m, L[52]);
+      L[53] = m2l_fma(-D[81], m, L[53]);
+      L[54] = m2l_fma(-D[82], m, L[54]);
+      L[55] = m2l_fma(-D[83], m, L[55]);
+    }
+    { const T m = __ldg(Ms + 4);
+      L[0] = m2l_fma(D[4], m, L[0]);
+      L[1] = m2l_fma(-D[10], m, L[1]);
+      L[2] = m2l_fma(-D[11], m, L[2]);
+      L[3] = m2l_fma(-D[12], m, L[3]);
+      L[4] = m2l_fma(D[20], m, L[4]);
+      L[5] = m2l_fma(D[21], m, L[5]);
+      L[6] = m2l_fma(D[22], m, L[6]);
+      L[7] = m2l_fma(D[23], m, L[7]);
+      L[8] = m2l_fma(D[24], m, L[8]);
+      L[9] = m2l_fma(D[25], m, L[9]);
+      L[10] = m2l_fma(-D[35], m, L[10]);
+      L[11] = m2l_fma(-D[36], m, L[11]);
+      L[12] = m2l_fma(-D[37], m, L[12]);
+      L[13] = m2l_fma(-D[38], m, L[13]);
+      L[14] = m2l_fma(-D[39], m, L[14]);
+      L[15] = m2l_fma(-D[40], m, L[15]);
+      L[16] = m2l_fma(-D[41], m, L[16]);
+      L[17] = m2l_fma(-D[42], m, L[17]);
+      L[18] = m2l_fma(-D[43], m, L[18]);
+      L[19] = m2l_fma(-D[44], m, L[19]);
+      L[20] = m2l_fma(D[56], m, L[20]);
+      L[21] = m2l_fma(D[57], m, L[21]);
+      L[22] = m2l_fma(D[58], m, L[22]);
+      L[23] = m2l_fma(D[59], m, L[23]);
+      L[24] = m2l_fma(D[60], m, L[24]);
+      L[25] = m2l_fma(D[61], m, L[25]);
+      L[26] = m2l_fma(D[62], m, L[26]);
+      L[27] = m2l_fma(D[63], m, L[27]);
+      L[28] = m2l_fma(D[64], m, L[28]);
+      L[29] = m2l_fma(D[65], m, L[29]);
+      L[30] = m2l_fma(D[66], m, L[30]);
+      L[31] = m2l_fma(D[67], m, L[31]);
+      L[32] = m2l_fma(D[68], m, L[32]);
+      L[33] = m2l_fma(D[69], m, L[33]);
+      L[34] = m2l_fma(D[70], m, L[34]);
+    }
+    { const T m = __ldg(Ms + 5);
+      L[0] = m2l_fma(D[5], m, L[0]);
+      L[1] = m2l_fma(-D[11], m, L[1]);
+      L[2] = m2l_fma(-D[13], m, L[2]);
+      L[3] = m2l_fma(-D[14], m, L[3]);
+      L[4] = m2l_fma(D[21], m, L[4]);
+      L[5] = m2l_fma(D[23], m, L[5]);
+      L[6] = m2l_fma(D[24], m, L[6]);
+      L[7] = m2l_fma(D[26], m, L[7]);
+      L[8] = m2l_fma(D[27], m, L[8]);
+      L[9] = m2l_fma(D[28], m, L[9]);
+      L[10] = m2l_fma(-D[36], m, L[10]);
+      L[11] = m2l_fma(-D[38], m, L[11]);
+      L[12] = m2l_fma(-D[39], m, L[12]);
+      L[13] = m2l_fma(-D[41], m, L[13]);
+      L[14] = m2l_fma(-D[42], m, L[14]);
+      L[15] = m2l_fma(-D[43], m, L[15]);
+      L[16] = m2l_fma(-D[45], m, L[16]);
+      L[17] = m2l_fma(-D[46], m, L[17]);
+      L[18] = m2l_fma(-D[47], m, L[18]);
+      L[19] = m2l_fma(-D[48], m, L[19]);
+      L[20] = m2l_fma(D[57], m, L[20]);
+      L[21] = m2l_fma(D[59], m, L[21]);
+      L[22] = m2l_fma(D[60], m, L[22]);
+      L[23] = m2l_fma(D[62], m, L[23]);
+      L[24] = m2l_fma(D[63], m, L[24]);
+      L[25] = m2l_fma(D[64], m, L[25]);
+      L[26] = m2l_fma(D[66], m, L[26]);
+      L[27] = m2l_fma(D[67], m, L[27]);
+      L[28] = m2l_fma(D[68], m, L[28]);
+      L[29] = m2l_fma(D[69], m, L[29]);
+      L[30] = m2l_fma(D[71], m, L[30]);
+      L[31] = m2l_fma(D[72], m, L[31]);
+      L[32] = m2l_fma(D[73], m, L[32]);
+      L[33] = m2l_fma(D[74], m, L[33]);
+      L[34] = m2l_fma(D[75], m, L[34]);
+    }
+    { const T m = __ldg(Ms + 6);
+      L[0] = m2l_fma(D[6], m, L[0]);
+      L[1] = m2l_fma(-D[12], m, L[1]);
+      L[2] = m2l_fma(-D[14], m, L[2]);
+      L[3] = m2l_fma(-D[15], m, L[3]);
+      L[4] = m2l_fma(D[22], m, L[4]);
+      L[5] = m2l_fma(D[24], m, L[5]);
+      L[6] = m2l_fma(D[25], m, L[6]);
+      L[7] = m2l_fma(D[27], m, L[7]);
+      L[8] = m2l_fma(D[28], m, L[8]);
+      L[9] = m2l_fma(D[29], m, L[9]);
+      L[10] = m2l_fma(-D[37], m, L[10]);
+      L[11] = m2l_fma(-D[39], m, L[11]);
+      L[12] = m2l_fma(-D[40], m, L[12]);
+      L[13] = m2l_fma(-D[42], m, L[13]);
+      L[14] = m2l_fma(-D[43], m, L[14]);
+      L[15] = m2l_fma(-D[44], m, L[15]);
+      L[16] = m2l_fma(-D[46], m, L[16]);
+      L[17] = m2l_fma(-D[47], m, L[17]);
+      L[18] = m2l_fma(-D[48], m, L[18]);
+      L[19] = m2l_fma(-D[49], m, L[19]);
+      L[20] = m2l_fma(D[58], m, L[20]);
+      L[21] = m2l_fma(D[60], m, L[21]);
+      L[22] = m2l_fma(D[61], m, L[22]);
+      L[23] = m2l_fma(D[63], m, L[23]);
+      L[24] = m2l_fma(D[64], m, L[24]);
+      L[25] = m2l_fma(D[65], m, L[25]);
+      L[26] = m2l_fma(D[67], m, L[26]);
+      L[27] = m2l_fma(D[68], m, L[27]);
+      L[28] = m2l_fma(D[69], m, L[28]);
+      L[29] = m2l_fma(D[70], m, L[29]);
+      L[30] = m2l_fma(D[72], m, L[30]);
+      L[31] = m2l_fma(D[73], m, L[31]);
+      L[32] = m2l_fma(D[74], m, L[32]);
+      L[33] = m2l_fma(D[75], m, L[33]);
+      L[34] = m2l_fma(D[76], m, L[34]);
+    }
+    { const T m = __ldg(Ms + 7);
+      L[0] = m2l_fma(D[7], m, L[0]);
+      L[1] = m2l_fma(-D[13], m, L[1]);
+      L[2] = m2l_fma(-D[16], m, L[2]);
+      L[3] = m2l_fma(-D[17], m, L[3]);
+      L[4] = m2l_fma(D[23], m, L[4]);
+      L[5] = m2l_fma(D[26], m, L[5]);
+      L[6] = m2l_fma(D[27], m, L[6]);
+      L[7] = m2l_fma(D[30], m, L[7]);
+      L[8] = m2l_fma(D[31], m, L[8]);
+      L[9] = m2l_fma(D[32], m, L[9]);
+      L[10] = m2l_fma(-D[38], m, L[10]);
+      L[11] = m2l_fma(-D[41], m, L[11]);
+      L[12] = m2l_fma(-D[42], m, L[12]);
+      L[13] = m2l_fma(-D[45], m, L[13]);
+      L[14] = m2l_fma(-D[46], m, L[14]);
+      L[15] = m2l_fma(-D[47], m, L[15]);
+      L[16] = m2l_fma(-D[50], m, L[16]);
+      L[17] = m2l_fma(-D[51], m, L[17]);
+      L[18] = m2l_fma(-D[52], m, L[18]);
+      L[19] = m2l_fma(-D[53], m, L[19]);
+      L[20] = m2l_fma(D[59], m, L[20]);
+      L[21] = m2l_fma(D[62], m, L[21]);
+      L[22] = m2l_fma(D[63], m, L[22]);
+      L[23] = m2l_fma(D[66], m, L[23]);
+      L[24] = m2l_fma(D[67], m, L[24]);
+      L[25] = m2l_fma(D[68], m, L[25]);
+      L[26] = m2l_fma(D[71], m, L[26]);
+      L[27] = m2l_fma(D[72], m, L[27]);
+      L[28] = m2l_fma(D[73], m, L[28]);
+      L[29] = m2l_fma(D[74], m, L[29]);
+      L[30] = m2l_fma(D[77], m, L[30]);
+      L[31] = m2l_fma(D[78], m, L[31]);
+      L[32] = m2l_fma(D[79], m, L[32]);
+      L[33] = m2l_fma(D[80], m, L[33]);
+      L[34] = m2l_fma(D[81], m, L[34]);
+    }
+    { const T m = __ldg(Ms + 8);
+      L[0] = m2l_fma(D[8], m, L[0]);
+      L[1] = m2l_fma(-D[14], m, L[1]);
+      L[2] = m2l_fma(-D[17], m, L[2]);
+      L[3] = m2l_fma(-D[18], m, L[3]);
+      L[4] = m2l_fma(D[24], m, L[4]);
+      L[5] = m2l_fma(D[27], m, L[5]);
+      L[6] = m2l_fma(D[28], m, L[6]);
+      L[7] = m2l_fma(D[31], m, L[7]);
+      L[8] = m2l_fma(D[32], m, L[8]);
+      L[9] = m2l_fma(D[33], m, L[9]);
+      L[10] = m2l_fma(-D[39], m, L[10]);
+      L[11] = m2l_fma(-D[42], m, L[11]);
+      L[12] = m2l_fma(-D[43], m, L[12]);
+      L[13] = m2l_fma(-D[46], m, L[13]);
+      L[14] = m2l_fma(-D[47], m, L[14]);
+      L[15] = m2l_fma(-D[48], m, L[15]);
+      L[16] = m2l_fma(-D[51], m, L[16]);
+      L[17] = m2l_fma(-D[52], m, L[17]);
+      L[18] = m2l_fma(-D[53], m, L[18]);
+      L[19] = m2l_fma(-D[54], m, L[19]);
+      L[20] = m2l_fma(D[60], m, L[20]);
+      L[21] = m2l_fma(D[63], m, L[21]);
+      L[22] = m2l_fma(D[64], m, L[22]);
+      L[23] = m2l_fma(D[67], m, L[23]);
+      L[24] = m2l_fma(D[68], m, L[24]);
+      L[25] = m2l_fma(D[69], m, L[25]);
+      L[26] = m2l_fma(D[72], m, L[26]);
+      L[27] = m2l_fma(D[73], m, L[27]);
+      L[28] = m2l_fma(D[74], m, L[28]);
+      L[29] = m2l_fma(D[75], m, L[29]);
+      L[30] = m2l_fma(D[78], m, L[30]);
+      L[31] = m2l_fma(D[79], m, L[31]);
+      L[32] = m2l_fma(D[80], m, L[32]);
+      L[33] = m2l_fma(D[81], m, L[33]);
+      L[34] = m2l_fma(D[82], m, L[34]);
+    }
+    { const T m = __ldg(Ms + 9);
+      L[0] = m2l_fma(D[9], m, L[0]);
+      L[1] = m2l_fma(-D[15], m, L[1]);
+      L[2] = m2l_fma(-D[18], m, L[2]);
+      L[3] = m2l_fma(-D[19], m, L[3]);
+      L[4] = m2l_fma(D[25], m, L[4]);
+      L[5] = m2l_fma(D[28], m, L[5]);
+      L[6] = m2l_fma(D[29], m, L[6]);
+      L[7] = m2l_fma(D[32], m, L[7]);
+      L[8] = m2l_fma(D[33], m, L[8]);
+      L[9] = m2l_fma(D[34], m, L[9]);
+      L[10] = m2l_fma(-D[40], m, L[10]);
+      L[11] = m2l_fma(-D[43], m, L[11]);
+      L[12] = m2l_fma(-D[44], m, L[12]);
+      L[13] = m2l_fma(-D[47], m, L[13]);
+      L[14] = m2l_fma(-D[48], m, L[14]);
+      L[15] = m2l_fma(-D[49], m, L[15]);
+      L[16] = m2l_fma(-D[52], m, L[16]);
+      L[17] = m2l_fma(-D[53], m, L[17]);
+      L[18] = m2l_fma(-D[54], m, L[18]);
+      L[19] = m2l_fma(-D[55], m, L[19]);
+      L[20] = m2l_fma(D[61], m, L[20]);
+      L[21] = m2l_fma(D[64], m, L[21]);
+      L[22] = m2l_fma(D[65], m, L[22]);
+      L[23] = m2l_fma(D[68], m, L[23]);
+      L[24] = m2l_fma(D[69], m, L[24]);
+      L[25] = m2l_fma(D[70], m, L[25]);
+      L[26] = m2l_fma(D[73], m, L[26]);
+      L[27] = m2l_fma(D[74], m, L[27]);
+      L[28] = m2l_fma(D[75], m, L[28]);
+      L[29] = m2l_fma(D[76], m, L[29]);
+      L[30] = m2l_fma(D[79], m, L[30]);
+      L[31] = m2l_fma(D[80], m, L[31]);
+      L[32] = m2l_fma(D[81], m, L[32]);
+      L[33] = m2l_fma(D[82], m, L[33]);
+      L[34] = m2l_fma(D[83], m, L[34]);
+    }
+    { const T m = __ldg(Ms + 10);
+      L[0] = m2l_fma(D[10], m, L[0]);
+      L[1] = m2l_fma(-D[20], m, L[1]);
+      L[2] = m2l_fma(-D[21], m, L[2]);
+      L[3] = m2l_fma(-D[22], m, L[3]);
+      L[4] = m2l_fma(D[35], m, L[4]);
+      L[5] = m2l_fma(D[36], m, L[5]);
+      L[6] = m2l_fma(D[37], m, L[6]);
+      L[7] = m2l_fma(D[38], m, L[7]);
+      L[8] = m2l_fma(D[39], m, L[8]);
+      L[9] = m2l_fma(D[40], m, L[9]);
+      L[10] = m2l_fma(-D[56], m, L[10]);
+      L[11] = m2l_fma(-D[57], m, L[11]);
+      L[12] = m2l_fma(-D[58], m, L[12]);
+      L[13] = m2l_fma(-D[59], m, L[13]);
+      L[14] = m2l_fma(-D[60], m, L[14]);
+      L[15] = m2l_fma(-D[61], m, L[15]);
+      L[16] = m2l_fma(-D[62], m, L[16]);
+      L[17] = m2l_fma(-D[63], m, L[17]);
+      L[18] = m2l_fma(-D[64], m, L[18]);
+      L[19] = m2l_fma(-D[65], m, L[19]);
+    }
+    { const T m = __ldg(Ms + 11);
+      L[0] = m2l_fma(D[11], m, L[0]);
+      L[1] = m2l_fma(-D[21], m, L[1]);
+      L[2] = m2l_fma(-D[23], m, L[2]);
+      L[3] = m2l_fma(-D[24], m, L[3]);
+      L[4] = m2l_fma(D[36], m, L[4]);
+      L[5] = m2l_fma(D[38], m, L[5]);
+      L[6] = m2l_fma(D[39], m, L[6]);
+      L[7] = m2l_fma(D[41], m, L[7]);
+      L[8] = m2l_fma(D[42], m, L[8]);
+      L[9] = m2l_fma(D[43], m, L[9]);
+      L[10] = m2l_fma(-D[57], m, L[10]);
+      L[11] = m2l_fma(-D[59], m, L[11]);
+      L[12] = m2l_fma(-D[60], m, L[12]);
+      L[13] = m2l_fma(-D[62], m, L[13]);
+      L[14] = m2l_fma(-D[63], m, L[14]);
+      L[15] = m2l_fma(-D[64], m, L[15]);
+      L[16] = m2l_fma(-D[66], m, L[16]);
+      L[17] = m2l_fma(-D[67], m, L[17]);
+      L[18] = m2l_fma(-D[68], m, L[18]);
+      L[19] = m2l_fma(-D[69], m, L[19]);
+    }
+    { const T m = __ldg(Ms + 12);
+      L[0] = m2l_fma(D[12], m, L[0]);
+      L[1] = m2l_fma(-D[22], m, L[1]);
+      L[2] = m2l_fma(-D[24], m, L[2]);
+      L[3] = m2l_fma(-D[25], m, L[3]);
+      L[4] = m2l_fma(D[37], m, L[4]);
+      L[5] = m2l_fma(D[39], m, L[5]);
+      L[6] = m2l_fma(D[40], m, L[6]);
+      L[7] = m2l_fma(D[42], m, L[7]);
+      L[8] = m2l_fma(D[43], m, L[8]);
+      L[9] = m2l_fma(D[44], m, L[9]);
+      L[10] = m2l_fma(-D[58], m, L[10]);
+      L[11] = m2l_fma(-D[60], m, L[11]);
+      L[12] = m2l_fma(-D[61], m, L[12]);
+      L[13] = m2l_fma(-D[63], m, L[13]);
+      L[14] = m2l_fma(-D[64], m, L[14]);
+      L[15] = m2l_fma(-D[65], m, L[15]);
+      L[16] = m2l_fma(-D[67], m, L[16]);
+      L[17] = m2l_fma(-D[68], m, L[17]);
+      L[18] = m2l_fma(-D[69], m, L[18]);
+      L[19] = m2l_fma(-D[70], m, L[19]);
+    }
+    { const T m = __ldg(Ms + 13);
+      L[0] = m2l_fma(D[13], m, L[0]);
+      L[1] = m2l_fma(-D[23], m, L[1]);
+      L[2] = m2l_fma(-D[26], m, L[2]);
+      L[3] = m2l_fma(-D[27], m, L[3]);
+      L[4] = m2l_fma(D[38], m, L[4]);
+      L[5] = m2l_fma(D[41], m, L[5]);
+      L[6] = m2l_fma(D[42], m, L[6]);
+      L[7] = m2l_fma(D[45], m, L[7]);
+      L[8] = m2l_fma(D[46], m, L[8]);
+      L[9] = m2l_fma(D[47], m, L[9]);
+      L[10] = m2l_fma(-D[59], m, L[10]);
+      L[11] = m2l_fma(-D[62], m, L[11]);
+      L[12] = m2l_fma(-D[63], m, L[12]);
+      L[13] = m2l_fma(-D[66], m, L[13]);
+      L[14] = m2l_fma(-D[67], m, L[14]);
+      L[15] = m2l_fma(-D[68], m, L[15]);
+      L[16] = m2l_fma(-D[71], m, L[16]);
+      L[17] = m2l_fma(-D[72], m, L[17]);
+      L[18] = m2l_fma(-D[73], m, L[18]);
+      L[19] = m2l_fma(-D[74], m, L[19]);
+    }
+    { const T m = __ldg(Ms + 14);
+      L[0] = m2l_fma(D[14], m, L[0]);
+      L[1] = m2l_fma(-D[24], m, L[1]);
+      L[2] = m2l_fma(-D[27], m, L[2]);
+      L[3] = m2l_fma(-D[28], m, L[3]);
+      L[4] = m2l_fma(D[39], m, L[4]);
+      L[5] = m2l_fma(D[42], m, L[5]);
+      L[6] = m2l_fma(D[43], m, L[6]);
+      L[7] = m2l_fma(D[46], m, L[7]);
+      L[8] = m2l_fma(D[47], m, L[8]);
+      L[9] = m2l_fma(D[48], m, L[9]);
+      L[10] = m2l_fma(-D[60], m, L[10]);
+      L[11] = m2l_fma(-D[63], m, L[11]);
+      L[12] = m2l_fma(-D[64], m, L[12]);
+      L[13] = m2l_fma(-D[67], m, L[13]);
+      L[14] = m2l_fma(-D[68], m, L[14]);
+      L[15] = m2l_fma(-D[69], m, L[15]);
+      L[16] = m2l_fma(-D[72], m, L[16]);
+      L[17] = m2l_fma(-D[73], m, L[17]);
+      L[18] = m2l_fma(-D[74], m, L[18]);
+      L[19] = m2l_fma(-D[75], m, L[19]);
+    }
+    { const T m = __ldg(Ms + 15);
+      L[0] = m2l_fma(D[15], m, L[0]);
+      L[1] = m2l_fma(-D[25], m, L[1]);
+      L[2] = m2l_fma(-D[28], m, L[2]);
+      L[3] = m2l_fma(-D[29], m, L[3]);
+      L[4] = m2l_fma(D[40], m, L[4]);
+      L[5] = m2l_fma(D[43], m, L[5]);
+      L[6] = m2l_fma(D[44], m, L[6]);
+      L[7] = m2l_fma(D[47], m, L[7]);
+      L[8] = m2l_fma(D[48], m, L[8]);
+      L[9] = m2l_fma(D[49], m, L[9]);
+      L[10] = m2l_fma(-D[61], m, L[10]);
+      L[11] = m2l_fma(-D[64], m, L[11]);
+      L[12] = m2l_fma(-D[65], m, L[12]);
+      L[13] = m2l_fma(-D[68], m, L[13]);
+      L[14] = m2l_fma(-D[69], m, L[14]);
+      L[15] = m2l_fma(-D[70], m, L[15]);
+      L[16] = m2l_fma(-D[73], m, L[16]);
+      L[17] = m2l_fma(-D[74], m, L[17]);
+      L[18] = m2l_fma(-D[75], m, L[18]);
+      L[19] = m2l_fma(-D[76], m, L[19]);
+    }
+    { const T m = __ldg(Ms + 16);
+      L[0] = m2l_fma(D[16], m, L[0]);
+      L[1] = m2l_fma(-D[26], m, L[1]);
+      L[2] = m2l_fma(-D[30], m, L[2]);
+      L[3] = m2l_fma(-D[31], m, L[3]);
+      L[4] = m2l_fma(D[41], m, L[4]);
+      L[5] = m2l_fma(D[45], m, L[5]);
+      L[6] = m2l_fma(D[46], m, L[6]);
+      L[7] = m2l_fma(D[50], m, L[7]);
+      L[8] = m2l_fma(D[51], m, L[8]);
+      L[9] = m2l_fma(D[52], m, L[9]);
+      L[10] = m2l_fma(-D[62], m, L[10]);
+      L[11] = m2l_fma(-D[66], m, L[11]);
+      L[12] = m2l_fma(-D[67], m, L[12]);
+      L[13] = m2l_fma(-D[71], m, L[13]);
+      L[14] = m2l_fma(-D[72], m, L[14]);
+      L[15] = m2l_fma(-D[73], m, L[15]);
+      L[16] = m2l_fma(-D[77], m, L[16]);
+      L[17] = m2l_fma(-D[78], m, L[17]);
+      L[18] = m2l_fma(-D[79], m, L[18]);
+      L[19] = m2l_fma(-D[80], m, L[19]);
+    }
+    { const T m = __ldg(Ms + 17);
+      L[0] = m2l_fma(D[17], m, L[0]);
+      L[1] = m2l_fma(-D[27], m, L[1]);
+      L[2] = m2l_fma(-D[31], m, L[2]);
+      L[3] = m2l_fma(-D[32], m, L[3]);
+      L[4] = m2l_fma(D[42], m, L[4]);
+      L[5] = m2l_fma(D[46], m, L[5]);
+      L[6] = m2l_fma(D[47], m, L[6]);
+      L[7] = m2l_fma(D[51], m, L[7]);
+      L[8] = m2l_fma(D[52], m, L[8]);
+      L[9] = m2l_fma(D[53], m, L[9]);
+      L[10] = m2l_fma(-D[63], m, L[10]);
+      L[11] = m2l_fma(-D[67], m, L[11]);
+      L[12] = m2l_fma(-D[68], m, L[12]);
+      L[13] = m2l_fma(-D[72], m, L[13]);
+      L[14] = m2l_fma(-D[73], m, L[14]);
+      L[15] = m2l_fma(-D[74], m, L[15]);
+      L[16] = m2l_fma(-D[78], m, L[16]);
+      L[17] = m2l_fma(-D[79], m, L[17]);
+      L[18] = m2l_fma(-D[80], m, L[18]);
+      L[19] = m2l_fma(-D[81], m, L[19]);
+    }
+    { const T m = __ldg(Ms + 18);
+      L[0] = m2l_fma(D[18], m, L[0]);
+      L[1] = m2l_fma(-D[28], m, L[1]);
+      L[2] = m2l_fma(-D[32], m, L[2]);
+      L[3] = m2l_fma(-D[33], m, L[3]);
+      L[4] = m2l_fma(D[43], m, L[4]);
+      L[5] = m2l_fma(D[47], m, L[5]);
+      L[6] = m2l_fma(D[48], m, L[6]);
+      L[7] = m2l_fma(D[52], m, L[7]);
+      L[8] = m2l_fma(D[53], m, L[8]);
+      L[9] = m2l_fma(D[54], m, L[9]);
+      L[10] = m2l_fma(-D[64], m, L[10]);
+      L[11] = m2l_fma(-D[68], m, L[11]);
+      L[12] = m2l_fma(-D[69], m, L[12]);
+      L[13] = m2l_fma(-D[73], m, L[13]);
+      L[14] = m2l_fma(-D[74], m, L[14]);
+      L[15] = m2l_fma(-D[75], m, L[15]);
+      L[16] = m2l_fma(-D[79], m, L[16]);
+      L[17] = m2l_fma(-D[80], m, L[17]);
+      L[18] = m2l_fma(-D[81], m, L[18]);
+      L[19] = m2l_fma(-D[82], m, L[19]);
+    }
+    { const T m = __ldg(Ms + 19);
+      L[0] = m2l_fma(D[19], m, L[0]);
+      L[1] = m2l_fma(-D[29], m, L[1]);
+      L[2] = m2l_fma(-D[33], m, L[2]);
+      L[3] = m2l_fma(-D[34], m, L[3]);
+      L[4] = m2l_fma(D[44], m, L[4]);
+      L[5] = m2l_fma(D[48], m, L[5]);
+      L[6] = m2l_fma(D[49], m, L[6]);
+      L[7] = m2l_fma(D[53], m, L[7]);
+      L[8] = m2l_fma(D[54], m, L[8]);
+      L[9] = m2l_fma(D[55], m, L[9]);
+      L[10] = m2l_fma(-D[65], m, L[10]);
+      L[11] = m2l_fma(-D[69], m, L[11]);
+      L[12] = m2l_fma(-D[70], m, L[12]);
+      L[13] = m2l_fma(-D[74], m, L[13]);
+      L[14] = m2l_fma(-D[75], m, L[14]);
+      L[15] = m2l_fma(-D[76], m, L[15]);
+      L[16] = m2l_fma(-D[80], m, L[16]);
+      L[17] = m2l_fma(-D[81], m, L[17]);
+      L[18] = m2l_fma(-D[82], m, L[18]);
+      L[19] = m2l_fma(-D[83], m, L[19]);
+    }
+    { const T m = __ldg(Ms + 20);
+      L[0] = m2l_fma(D[20], m, L[0]);
+      L[1] = m2l_fma(-D[35], m, L[1]);
+      L[2] = m2l_fma(-D[36], m, L[2]);
+      L[3] = m2l_fma(-D[37], m, L[3]);
+      L[4] = m2l_fma(D[56], m, L[4]);
+      L[5] = m2l_fma(D[57], m, L[5]);
+      L[6] = m2l_fma(D[58], m, L[6]);
+      L[7] = m2l_fma(D[59], m, L[7]);
+      L[8] = m2l_fma(D[60], m, L[8]);
+      L[9] = m2l_fma(D[61], m, L[9]);
+    }
+    { const T m = __ldg(Ms + 21);
+      L[0] = m2l_fma(D[21], m, L[0]);
+      L[1] = m2l_fma(-D[36], m, L[1]);
+      L[2] = m2l_fma(-D[38], m, L[2]);
+      L[3] = m2l_fma(-D[39], m, L[3]);
+      L[4] = m2l_fma(D[57], m, L[4]);
+      L[5] = m2l_fma(D[59], m, L[5]);
+      L[6] = m2l_fma(D[60], m, L[6]);
+      L[7] = m2l_fma(D[62], m, L[7]);
+      L[8] = m2l_fma(D[63], m, L[8]);
+      L[9] = m2l_fma(D[64], m, L[9]);
+    }
+    { const T m = __ldg(Ms + 22);
+      L[0] = m2l_fma(D[22], m, L[0]);
+      L[1] = m2l_fma(-D[37], m, L[1]);
+      L[2] = m2l_fma(-D[39], m, L[2]);
+      L[3] = m2l_fma(-D[40], m, L[3]);
+      L[4] = m2l_fma(D[58], m, L[4]);
+      L[5] = m2l_fma(D[60], m, L[5]);
+      L[6] = m2l_fma(D[61], m, L[6]);
+      L[7] = m2l_fma(D[63], m, L[7]);
+      L[8] = m2l_fma(D[64], m, L[8]);
+      L[9] = m2l_fma(D[65], m, L[9]);
+    }
+    { const T m = __ldg(Ms + 23);
+      L[0] = m2l_fma(D[23], m, L[0]);
+      L[1] = m2l_fma(-D[38], m, L[1]);
+      L[2] = m2l_fma(-D[41], m, L[2]);
+      L[3] = m2l_fma(-D[42], m, L[3]);
+      L[4] = m2l_fma(D[59], m, L[4]);
+      L[5] = m2l_fma(D[62], m, L[5]);
+      L[6] = m2l_fma(D[63], m, L[6]);
+      L[7] = m2l_fma(D[66], m, L[7]);
+      L[8] = m2l_fma(D[67], m, L[8]);
+      L[9] = m2l_fma(D[68], m, L[9]);
+    }
+    { const T m = __ldg(Ms + 24);
+      L[0] = m2l_fma(D[24], m, L[0]);
+      L[1] = m2l_fma(-D[39], m, L[1]);
+      L[2] = m2l_fma(-D[42], m, L[2]);
+      L[3] = m2l_fma(-D[43], m, L[3]);
+      L[4] = m2l_fma(D[60], m, L[4]);
+      L[5] = m2l_fma(D[63], m, L[5]);
+      L[6] = m2l_fma(D[64], m, L[6]);
+      L[7] = m2l_fma(D[67], m, L[7]);
+      L[8] = m2l_fma(D[68], m, L[8]);
+      L[9] = m2l_fma(D[69], m, L[9]);
+    }
+    { const T m = __ldg(Ms + 25);
+      L[0] = m2l_fma(D[25], m, L[0]);
+      L[1] = m2l_fma(-D[40], m, L[1]);
+      L[2] = m2l_fma(-D[43], m, L[2]);
+      L[3] = m2l_fma(-D[44], m, L[3]);
+      L[4] = m2l_fma(D[61], m, L[4]);
+      L[5] = m2l_fma(D[64], m, L[5]);
+      L[6] = m2l_fma(D[65], m, L[6]);
+      L[7] = m2l_fma(D[68], m, L[7]);
+      L[8] = m2l_fma(D[69], m, L[8]);
+      L[9] = m2l_fma(D[70], m, L[9]);
+    }
+    { const T m = __ldg(Ms + 26);
+      L[0] = m2l_fma(D[26], m, L[0]);
+      L[1] = m2l_fma(-D[41], m, L[1]);
+      L[2] = m2l_fma(-D[45], m, L[2]);
+      L[3] = m2l_fma(-D[46], m, L[3]);
+      L[4] = m2l_fma(D[62], m, L[4]);
+      L[5] = m2l_fma(D[66], m, L[5]);
+      L[6] = m2l_fma(D[67], m, L[6]);
+      L[7] = m2l_fma(D[71], m, L[7]);
+      L[8] = m2l_fma(D[72], m, L[8]);
+      L[9] = m2l_fma(D[73], m, L[9]);
+    }
+    { const T m = __ldg(Ms + 27);
+      L[0] = m2l_fma(D[27], m, L[0]);
+      L[1] = m2l_fma(-D[42], m, L[1]);
+      L[2] = m2l_fma(-D[46], m, L[2]);
+      L[3] = m2l_fma(-D[47], m, L[3]);
+      L[4] = m2l_fma(D[63], m, L[4]);
+      L[5] = m2l_fma(D[67], m, L[5]);
+      L[6] = m2l_fma(D[68], m, L[6]);
+      L[7] = m2l_fma(D[72], m, L[7]);
+      L[8] = m2l_fma(D[73], m, L[8]);
+      L[9] = m2l_fma(D[74], m, L[9]);
+    }
+    { const T m = __ldg(Ms + 28);
+      L[0] = m2l_fma(D[28], m, L[0]);
+      L[1] = m2l_fma(-D[43], m, L[1]);
+      L[2] = m2l_fma(-D[47], m, L[2]);
+      L[3] = m2l_fma(-D[48], m, L[3]);
+      L[4] = m2l_fma(D[64], m, L[4]);
+      L[5] = m2l_fma(D[68], m, L[5]);
+      L[6] = m2l_fma(D[69], m, L[6]);
+      L[7] = m2l_fma(D[73], m, L[7]);
+      L[8] = m2l_fma(D[74], m, L[8]);
+      L[9] = m2l_fma(D[75], m, L[9]);
+    }
+    { const T m = __ldg(Ms + 29);
+      L[0] = m2l_fma(D[29], m, L[0]);
+      L[1] = m2l_fma(-D[44], m, L[1]);
+      L[2] = m2l_fma(-D[48], m, L[2]);
+      L[3] = m2l_fma(-D[49], m, L[3]);
+      L[4] = m2l_fma(D[65], m, L[4]);
+      L[5] = m2l_fma(D[69], m, L[5]);
+      L[6] = m2l_fma(D[70], m, L[6]);
+      L[7] = m2l_fma(D[74], m, L[7]);
+      L[8] = m2l_fma(D[75], m, L[8]);
+      L[9] = m2l_fma(D[76], m, L[9]);
+    }
+    { const T m = __ldg(Ms + 30);
+      L[0] = m2l_fma(D[30], m, L[0]);
+      L[1] = m2l_fma(-D[45], m, L[1]);
+      L[2] = m2l_fma(-D[50], m, L[2]);
+      L[3] = m2l_fma(-D[51], m, L[3]);
+      L[4] = m2l_fma(D[66], m, L[4]);
+      L[5] = m2l_fma(D[71], m, L[5]);
+      L[6] = m2l_fma(D[72], m, L[6]);
+      L[7] = m2l_fma(D[77], m, L[7]);
+      L[8] = m2l_fma(D[78], m, L[8]);
+      L[9] = m2l_fma(D[79], m, L[9]);
+    }
+    { const T m = __ldg(Ms + 31);
+      L[0] = m2l_fma(D[31], m, L[0]);
+      L[1] = m2l_fma(-D[46], m, L[1]);
+      L[2] = m2l_fma(-D[51], m, L[2]);
+      L[3] = m2l_fma(-D[52], m, L[3]);
+      L[4] = m2l_fma(D[67], m, L[4]);
+      L[5] = m2l_fma(D[72], m, L[5]);
+      L[6] = m2l_fma(D[73], m, L[6]);
+      L[7] = m2l_fma(D[78], m, L[7]);
+      L[8] = m2l_fma(D[79], m, L[8]);
+      L[9] = m2l_fma(D[80], m, L[9]);
+    }
+    { const T m = __ldg(Ms + 32);
+      L[0] = m2l_fma(D[32], m, L[0]);
+      L[1] = m2l_fma(-D[47], m, L[1]);
+      L[2] = m2l_fma(-D[52], m, L[2]);
+      L[3] = m2l_fma(-D[53], m, L[3]);
+      L[4] = m2l_fma(D[68], m, L[4]);
+      L[5] = m2l_fma(D[73], m, L[5]);
+      L[6] = m2l_fma(D[74], m, L[6]);
+      L[7] = m2l_fma(D[79], m, L[7]);
+      L[8] = m2l_fma(D[80], m, L[8]);
+      L[9] = m2l_fma(D[81], m, L[9]);
+    }
+    { const T m = __ldg(Ms + 33);
+      L[0] = m2l_fma(D[33], m, L[0]);
+      L[1] = m2l_fma(-D[48], m, L[1]);
+      L[2] = m2l_fma(-D[53], m, L[2]);
+      L[3] = m2l_fma(-D[54], m, L[3]);
+      L[4] = m2l_fma(D[69], m, L[4]);
+      L[5] = m2l_fma(D[74], m, L[5]);
+      L[6] = m2l_fma(D[75], m, L[6]);
+      L[7] = m2l_fma(D[80], m, L[7]);
+      L[8] = m2l_fma(D[81], m, L[8]);
+      L[9] = m2l_fma(D[82], m, L[9]);
+    }
+    { const T m = __ldg(Ms + 34);
+      L[0] = m2l_fma(D[34], m, L[0]);
+      L[1] = m2l_fma(-D[49], m, L[1]);
+      L[2] = m2l_fma(-D[54], m, L[2]);
+      L[3] = m2l_fma(-D[55], m, L[3]);
+      L[4] = m2l_fma(D[70], m, L[4]);
+      L[5] = m2l_fma(D[75], m, L[5]);
+      L[6] = m2l_fma(D[76], m, L[6]);
+      L[7] = m2l_fma(D[81], m, L[7]);
+      L[8] = m2l_fma(D[82], m, L[8]);
+      L[9] = m2l_fma(D[83], m, L[9]);
+    }
+    { const T m = __ldg(Ms + 35);
+      L[0] = m2l_fma(D[35], m, L[0]);
+      L[1] = m2l_fma(-D[56], m, L[1]);
+      L[2] = m2l_fma(-D[57], m, L[2]);
+      L[3] = m2l_fma(-D[58], m, L[3]);
+    }
+    { const T m = __ldg(Ms + 36);
+      L[0] = m2l_fma(D[36], m, L[0]);
+      L[1] = m2l_fma(-D[57], m, L[1]);
+      L[2] = m2l_fma(-D[59], m, L[2]);
+      L[3] = m2l_fma(-D[60], m, L[3]);
+    }
+    { const T m = __ldg(Ms + 37);
+      L[0] = m2l_fma(D[37], m, L[0]);
+      L[1] = m2l_fma(-D[58], m, L[1]);
+      L[2] = m2l_fma(-D[60], m, L[2]);
+      L[3] = m2l_fma(-D[61], m, L[3]);
+    }
+    { const T m = __ldg(Ms + 38);
+      L[0] = m2l_fma(D[38], m, L[0]);
+      L[1] = m2l_fma(-D[59], m, L[1]);
+      L[2] = m2l_fma(-D[62], m, L[2]);
+      L[3] = m2l_fma(-D[63], m, L[3]);
+    }
+    { const T m = __ldg(Ms + 39);
+      L[0] = m2l_fma(D[39], m, L[0]);
+      L[1] = m2l_fma(-D[60], m, L[1]);
+      L[2] = m2l_fma(-D[63], m, L[2]);
+      L[3] = m2l_fma(-D[64], m, L[3]);
+    }
+    { const T m = __ldg(Ms + 40);
+      L[0] = m2l_fma(D[40], m, L[0]);
+      L[1] = m2l_fma(-D[61], m, L[1]);
+      L[2] = m2l_fma(-D[64], m, L[2]);
+      L[3] = m2l_fma(-D[65], m, L[3]);
+    }
+    { const T m = __ldg(Ms + 41);
+      L[0] = m2l_fma(D[41], m, L[0]);
+      L[1] = m2l_fma(-D[62], m, L[1]);
+      L[2] = m2l_fma(-D[66], m, L[2]);
+      L[3] = m2l_fma(-D[67], m, L[3]);
+    }
+    { const T m = __ldg(Ms + 42);
+      L[0] = m2l_fma(D[42], m, L[0]);
+      L[1] = m2l_fma(-D[63], m, L[1]);
+      L[2] = m2l_fma(-D[67], m, L[2]);
+      L[3] = m2l_fma(-D[68], m, L[3]);
+    }
+    { const T m = __ldg(Ms + 43);
+      L[0] = m2l_fma(D[43], m, L[0]);
+      L[1] = m2l_fma(-D[64], m, L[1]);
+      L[2] = m2l_fma(-D[68], m, L[2]);
+      L[3] = m2l_fma(-D[69], m, L[3]);
+    }
+    { const T m = __ldg(Ms + 44);
+      L[0] = m2l_fma(D[44], m, L[0]);
+      L[1] = m2l_fma(-D[65], m, L[1]);
+      L[2] = m2l_fma(-D[69], m, L[2]);
+      L[3] = m2l_fma(-D[70], m, L[3]);
+    }
+    { const T m = __ldg(Ms + 45);
+      L[0] = m2l_fma(D[45], m, L[0]);
+      L[1] = m2l_fma(-D[66], m, L[1]);
+      L[2] = m2l_fma(-D[71], m, L[2]);
+      L[3] = m2l_fma(-D[72], m, L[3]);
+    }
+    { const T m = __ldg(Ms + 46);
+      L[0] = m2l_fma(D[46], m, L[0]);
+      L[1] = m2l_fma(-D[67], m, L[1]);
+      L[2] = m2l_fma(-D[72], m, L[2]);
+      L[3] = m2l_fma(-D[73], m, L[3]);
+    }
+    { const T m = __ldg(Ms + 47);
+      L[0] = m2l_fma(D[47], m, L[0]);
+      L[1] = m2l_fma(-D[68], m, L[1]);
+      L[2] = m2l_fma(-D[73], m, L[2]);
+      L[3] = m2l_fma(-D[74], m, L[3]);
+    }
+    { const T m = __ldg(Ms + 48);
+      L[0] = m2l_fma(D[48], m, L[0]);
+      L[1] = m2l_fma(-D[69], m, L[1]);
+      L[2] = m2l_fma(-D[74], m, L[2]);
+      L[3] = m2l_fma(-D[75], m, L[3]);
+    }
+    { const T m = __ldg(Ms + 49);
+      L[0] = m2l_fma(D[49], m, L[0]);
+      L[1] = m2l_fma(-D[70], m, L[1]);
+      L[2] = m2l_fma(-D[75], m, L[2]);
+      L[3] = m2l_fma(-D[76], m, L[3]);
+    }
+    { const T m = __ldg(Ms + 50);
+      L[0] = m2l_fma(D[50], m, L[0]);
+      L[1] = m2l_fma(-D[71], m, L[1]);
+      L[2] = m2l_fma(-D[77], m, L[2]);
+      L[3] = m2l_fma(-D[78], m, L[3]);
+    }
+    { const T m = __ldg(Ms + 51);
+      L[0] = m2l_fma(D[51], m, L[0]);
+      L[1] = m2l_fma(-D[72], m, L[1]);
+      L[2] = m2l_fma(-D[78], m, L[2]);
+      L[3] = m2l_fma(-D[79], m, L[3]);
+    }
+    { const T m = __ldg(Ms + 52);
+      L[0] = m2l_fma(D[52], m, L[0]);
+      L[1] = m2l_fma(-D[73], m, L[1]);
+      L[2] = m2l_fma(-D[79], m, L[2]);
+      L[3] = m2l_fma(-D[80], m, L[3]);
+    }
+    { const T m = __ldg(Ms + 53);
+      L[0] = m2l_fma(D[53], m, L[0]);
+      L[1] = m2l_fma(-D[74], m, L[1]);
+      L[2] = m2l_fma(-D[80], m, L[2]);
+      L[3] = m2l_fma(-D[81], m, L[3]);
+    }
+    { const T m = __ldg(Ms + 54);
+      L[0] = m2l_fma(D[54], m, L[0]);
+      L[1] = m2l_fma(-D[75], m, L[1]);
+      L[2] = m2l_fma(-D[81], m, L[2]);
+      L[3] = m2l_fma(-D[82], m, L[3]);
+    }
+    { const T m = __ldg(Ms + 55);
+      L[0] = m2l_fma(D[55], m, L[0]);
+      L[1] = m2l_fma(-D[76], m, L[1]);
+      L[2] = m2l_fma(-D[82], m, L[2]);
+      L[3] = m2l_fma(-D[83], m, L[3]);
+    }
+    { const T m = __ldg(Ms + 56);
+      L[0] = m2l_fma(D[56], m, L[0]);
+    }
+    { const T m = __ldg(Ms + 57);
+      L[0] = m2l_fma(D[57], m, L[0]);
+    }
+    { const T m = __ldg(Ms + 58);
+      L[0] = m2l_fma(D[58], m, L[0]);
+    }
+    { const T m = __ldg(Ms + 59);
+      L[0] = m2l_fma(D[59], m, L[0]);
+    }
+    { const T m = __ldg(Ms + 60);
+      L[0] = m2l_fma(D[60], m, L[0]);
+    }
+    { const T m = __ldg(Ms + 61);
+      L[0] = m2l_fma(D[61], m, L[0]);
+    }
+    { const T m = __ldg(Ms + 62);
+      L[0] = m2l_fma(D[62], m, L[0]);
+    }
+    { const T m = __ldg(Ms + 63);
+      L[0] = m2l_fma(D[63], m, L[0]);
+    }
+    { const T m = __ldg(Ms + 64);
+      L[0] = m2l_fma(D[64], m, L[0]);
+    }
+    { const T m = __ldg(Ms + 65);
+      L[0] = m2l_fma(D[65], m, L[0]);
+    }
+    { const T m = __ldg(Ms + 66);
+      L[0] = m2l_fma(D[66], m, L[0]);
+    }
+    { const T m = __ldg(Ms + 67);
+      L[0] = m2l_fma(D[67], m, L[0]);
+    }
+    { const T m = __ldg(Ms + 68);
+      L[0] = m2l_fma(D[68], m, L[0]);
+    }
+    { const T m = __ldg(Ms + 69);
+      L[0] = m2l_fma(D[69], m, L[0]);
+    }
+    { const T m = __ldg(Ms + 70);
+      L[0] = m2l_fma(D[70], m, L[0]);
+    }
+    { const T m = __ldg(Ms + 71);
+      L[0] = m2l_fma(D[71], m, L[0]);
+    }
+    { const T m = __ldg(Ms + 72);
+      L[0] = m2l_fma(D[72], m, L[0]);
+    }
+    { const T m = __ldg(Ms + 73);
+      L[0] = m2l_fma(D[73], m, L[0]);
+    }
+    { const T m = __ldg(Ms + 74);
+      L[0] = m2l_fma(D[74], m, L[0]);
+    }
+    { const T m = __ldg(Ms + 75);
+      L[0] = m2l_fma(D[75], m, L[0]);
+    }
+    { const T m = __ldg(Ms + 76);
+      L[0] = m2l_fma(D[76], m, L[0]);
+    }
+    { const T m = __ldg(Ms + 77);
+      L[0] = m2l_fma(D[77], m, L[0]);
+    }
+    { const T m = __ldg(Ms + 78);
+      L[0] = m2l_fma(D[78], m, L[0]);
+    }
+    { const T m = __ldg(Ms + 79);
+      L[0] = m2l_fma(D[79], m, L[0]);
+    }
+    { const T m = __ldg(Ms + 80);
+      L[0] = m2l_fma(D[80], m, L[0]);
+    }
+    { const T m = __ldg(Ms + 81);
+      L[0] = m2l_fma(D[81], m, L[0]);
+    }
+    { const T m = __ldg(Ms + 82);
+      L[0] = m2l_fma(D[82], m, L[0]);
+    }
+    { const T m = __ldg(Ms + 83);
+      L[0] = m2l_fma(D[83], m, L[0]);
     }
 }
 
-__device__ __forceinline__ void m2l_side_a_forces_6(const float (&D)[84], const float *__restrict__ Ms, float rho, float (&L)[84])
+template <class T> __device__ __forceinline__ void m2l_side_a_forces_6(const T (&D)[84], const T *__restrict__ Ms, T rho, T (&L)[84])
 {
-    L[0] = 0.0f;
-    float rp = 1.0f;
-    { const float m = __ldg(Ms + 0) * rp;
+    L[0] = T(0);
+    T rp = T(1);
+    { const T m = __ldg(Ms + 0) * rp;
       L[1] = D[1] * m;
       L[2] = D[2] * m;
       L[3] = D[3] * m;
@@ -6854,883 +6859,883 @@ __device__ __forceinline__ void m2l_side_a_forces_6(const float (&D)[84], const 
       L[83] = D[83] * m;
     }
     rp *= rho;
-    { const float m = -__ldg(Ms + 1) * rp;
-      L[1] = fmaf(D[4], m, L[1]);
-      L[2] = fmaf(D[5], m, L[2]);
-      L[3] = fmaf(D[6], m, L[3]);
-      L[4] = fmaf(D[10], m, L[4]);
-      L[5] = fmaf(D[11], m, L[5]);
-      L[6] = fmaf(D[12], m, L[6]);
-      L[7] = fmaf(D[13], m, L[7]);
-      L[8] = fmaf(D[14], m, L[8]);
-      L[9] = fmaf(D[15], m, L[9]);
-      L[10] = fmaf(D[20], m, L[10]);
-      L[11] = fmaf(D[21], m, L[11]);
-      L[12] = fmaf(D[22], m, L[12]);
-      L[13] = fmaf(D[23], m, L[13]);
-      L[14] = fmaf(D[24], m, L[14]);
-      L[15] = fmaf(D[25], m, L[15]);
-      L[16] = fmaf(D[26], m, L[16]);
-      L[17] = fmaf(D[27], m, L[17]);
-      L[18] = fmaf(D[28], m, L[18]);
-      L[19] = fmaf(D[29], m, L[19]);
-      L[20] = fmaf(D[35], m, L[20]);
-      L[21] = fmaf(D[36], m, L[21]);
-      L[22] = fmaf(D[37], m, L[22]);
-      L[23] = fmaf(D[38], m, L[23]);
-      L[24] = fmaf(D[39], m, L[24]);
-      L[25] = fmaf(D[40], m, L[25]);
-      L[26] = fmaf(D[41], m, L[26]);
-      L[27] = fmaf(D[42], m, L[27]);
-      L[28] = fmaf(D[43], m, L[28]);
-      L[29] = fmaf(D[44], m, L[29]);
-      L[30] = fmaf(D[45], m, L[30]);
-      L[31] = fmaf(D[46], m, L[31]);
-      L[32] = fmaf(D[47], m, L[32]);
-      L[33] = fmaf(D[48], m, L[33]);
-      L[34] = fmaf(D[49], m, L[34]);
-      L[35] = fmaf(D[56], m, L[35]);
-      L[36] = fmaf(D[57], m, L[36]);
-      L[37] = fmaf(D[58], m, L[37]);
-      L[38] = fmaf(D[59], m, L[38]);
-      L[39] = fmaf(D[60], m, L[39]);
-      L[40] = fmaf(D[61], m, L[40]);
-      L[41] = fmaf(D[62], m, L[41]);
-      L[42] = fmaf(D[63], m, L[42]);
-      L[43] = fmaf(D[64], m, L[43]);
-      L[44] = fmaf(D[65], m, L[44]);
-      L[45] = fmaf(D[66], m, L[45]);
-      L[46] = fmaf(D[67], m, L[46]);
-      L[47] = fmaf(D[68], m, L[47]);
-      L[48] = fmaf(D[69], m, L[48]);
-      L[49] = fmaf(D[70], m, L[49]);
-      L[50] = fmaf(D[71], m, L[50]);
-      L[51] = fmaf(D[72], m, L[51]);
-      L[52] = fmaf(D[73], m, L[52]);
-      L[53] = fmaf(D[74], m, L[53]);
-      L[54] = fmaf(D[75], m, L[54]);
-      L[55] = fmaf(D[76], m, L[55]);
+    { const T m = -__ldg(Ms + 1) * rp;
+      L[1] = m2l_fma(D[4], m, L[1]);
+      L[2] = m2l_fma(D[5], m, L[2]);
+      L[3] = m2l_fma(D[6], m, L[3]);
+      L[4] = m2l_fma(D[10], m, L[4]);
+      L[5] = m2l_fma(D[11], m, L[5]);
+      L[6] = m2l_fma(D[12], m, L[6]);
+      L[7] = m2l_fma(D[13], m, L[7]);
+      L[8] = m2l_fma(D[14], m, L[8]);
+      L[9] = m2l_fma(D[15], m, L[9]);
+      L[10] = m2l_fma(D[20], m, L[10]);
+      L[11] = m2l_fma(D[21], m, L[11]);
+      L[12] = m2l_fma(D[22], m, L[12]);
+      L[13] = m2l_fma(D[23], m, L[13]);
+      L[14] = m2l_fma(D[24], m, L[14]);
+      L[15] = m2l_fma(D[25], m, L[15]);
+      L[16] = m2l_fma(D[26], m, L[16]);
+      L[17] = m2l_fma(D[27], m, L[17]);
+      L[18] = m2l_fma(D[28], m, L[18]);
+      L[19] = m2l_fma(D[29], m, L[19]);
+      L[20] = m2l_fma(D[35], m, L[20]);
+      L[21] = m2l_fma(D[36], m, L[21]);
+      L[22] = m2l_fma(D[37], m, L[22]);
+      L[23] = m2l_fma(D[38], m, L[23]);
+      L[24] = m2l_fma(D[39], m, L[24]);
+      L[25] = m2l_fma(D[40], m, L[25]);
+      L[26] = m2l_fma(D[41], m, L[26]);
+      L[27] = m2l_fma(D[42], m, L[27]);
+      L[28] = m2l_fma(D[43], m, L[28]);
+      L[29] = m2l_fma(D[44], m, L[29]);
+      L[30] = m2l_fma(D[45], m, L[30]);
+      L[31] = m2l_fma(D[46], m, L[31]);
+      L[32] = m2l_fma(D[47], m, L[32]);
+      L[33] = m2l_fma(D[48], m, L[33]);
+      L[34] = m2l_fma(D[49], m, L[34]);
+      L[35] = m2l_fma(D[56], m, L[35]);
+      L[36] = m2l_fma(D[57], m, L[36]);
+      L[37] = m2l_fma(D[58], m, L[37]);
+      L[38] = m2l_fma(D[59], m, L[38]);
+      L[39] = m2l_fma(D[60], m, L[39]);
+      L[40] = m2l_fma(D[61], m, L[40]);
+      L[41] = m2l_fma(D[62], m, L[41]);
+      L[42] = m2l_fma(D[63], m, L[42]);
+      L[43] = m2l_fma(D[64], m, L[43]);
+      L[44] = m2l_fma(D[65], m, L[44]);
+      L[45] = m2l_fma(D[66], m, L[45]);
+      L[46] = m2l_fma(D[67], m, L[46]);
+      L[47] = m2l_fma(D[68], m, L[47]);
+      L[48] = m2l_fma(D[69], m, L[48]);
+      L[49] = m2l_fma(D[70], m, L[49]);
+      L[50] = m2l_fma(D[71], m, L[50]);
+      L[51] = m2l_fma(D[72], m, L[51]);
+      L[52] = m2l_fma(D[73], m, L[52]);
+      L[53] = m2l_fma(D[74], m, L[53]);
+      L[54] = m2l_fma(D[75], m, L[54]);
+      L[55] = m2l_fma(D[76], m, L[55]);
     }
-    { const float m = -__ldg(Ms + 2) * rp;
-      L[1] = fmaf(D[5], m, L[1]);
-      L[2] = fmaf(D[7], m, L[2]);
-      L[3] = fmaf(D[8], m, L[3]);
-      L[4] = fmaf(D[11], m, L[4]);
-      L[5] = fmaf(D[13], m, L[5]);
-      L[6] = fmaf(D[14], m, L[6]);
-      L[7] = fmaf(D[16], m, L[7]);
-      L[8] = fmaf(D[17], m, L[8]);
-      L[9] = fmaf(D[18], m, L[9]);
-      L[10] = fmaf(D[21], m, L[10]);
-      L[11] = fmaf(D[23], m, L[11]);
-      L[12] = fmaf(D[24], m, L[12]);
-      L[13] = fmaf(D[26], m, L[13]);
-      L[14] = fmaf(D[27], m, L[14]);
-      L[15] = fmaf(D[28], m, L[15]);
-      L[16] = fmaf(D[30], m, L[16]);
-      L[17] = fmaf(D[31], m, L[17]);
-      L[18] = fmaf(D[32], m, L[18]);
-      L[19] = fmaf(D[33], m, L[19]);
-      L[20] = fmaf(D[36], m, L[20]);
-      L[21] = fmaf(D[38], m, L[21]);
-      L[22] = fmaf(D[39], m, L[22]);
-      L[23] = fmaf(D[41], m, L[23]);
-      L[24] = fmaf(D[42], m, L[24]);
-      L[25] = fmaf(D[43], m, L[25]);
-      L[26] = fmaf(D[45], m, L[26]);
-      L[27] = fmaf(D[46], m, L[27]);
-      L[28] = fmaf(D[47], m, L[28]);
-      L[29] = fmaf(D[48], m, L[29]);
-      L[30] = fmaf(D[50], m, L[30]);
-      L[31] = fmaf(D[51], m, L[31]);
-      L[32] = fmaf(D[52], m, L[32]);
-      L[33] = fmaf(D[53], m, L[33]);
-      L[34] = fmaf(D[54], m, L[34]);
-      L[35] = fmaf(D[57], m, L[35]);
-      L[36] = fmaf(D[59], m, L[36]);
-      L[37] = fmaf(D[60], m, L[37]);
-      L[38] = fmaf(D[62], m, L[38]);
-      L[39] = fmaf(D[63], m, L[39]);
-      L[40] = fmaf(D[64], m, L[40]);
-      L[41] = fmaf(D[66], m, L[41]);
-      L[42] = fmaf(D[67], m, L[42]);
-      L[43] = fmaf(D[68], m, L[43]);
-      L[44] = fmaf(D[69], m, L[44]);
-      L[45] = fmaf(D[71], m, L[45]);
-      L[46] = fmaf(D[72], m, L[46]);
-      L[47] = fmaf(D[73], m, L[47]);
-      L[48] = fmaf(D[74], m, L[48]);
-      L[49] = fmaf(D[75], m, L[49]);
-      L[50] = fmaf(D[77], m, L[50]);
-      L[51] = fmaf(D[78], m, L[51]);
-      L[52] = fmaf(D[79], m, L[52]);
-      L[53] = fmaf(D[80], m, L[53]);
-      L[54] = fmaf(D[81], m, L[54]);
-      L[55] = fmaf(D[82], m, L[55]);
+    { const T m = -__ldg(Ms + 2) * rp;
+      L[1] = m2l_fma(D[5], m, L[1]);
+      L[2] = m2l_fma(D[7], m, L[2]);
+      L[3] = m2l_fma(D[8], m, L[3]);
+      L[4] = m2l_fma(D[11], m, L[4]);
+      L[5] = m2l_fma(D[13], m, L[5]);
+      L[6] = m2l_fma(D[14], m, L[6]);
+      L[7] = m2l_fma(D[16], m, L[7]);
+      L[8] = m2l_fma(D[17], m, L[8]);
+      L[9] = m2l_fma(D[18], m, L[9]);
+      L[10] = m2l_fma(D[21], m, L[10]);
+      L[11] = m2l_fma(D[23], m, L[11]);
+      L[12] = m2l_fma(D[24], m, L[12]);
+      L[13] = m2l_fma(D[26], m, L[13]);
+      L[14] = m2l_fma(D[27], m, L[14]);
+      L[15] = m2l_fma(D[28], m, L[15]);
+      L[16] = m2l_fma(D[30], m, L[16]);
+      L[17] = m2l_fma(D[31], m, L[17]);
+      L[18] = m2l_fma(D[32], m, L[18]);
+      L[19] = m2l_fma(D[33], m, L[19]);
+      L[20] = m2l_fma(D[36], m, L[20]);
+      L[21] = m2l_fma(D[38], m, L[21]);
+      L[22] = m2l_fma(D[39], m, L[22]);
+      L[23] = m2l_fma(D[41], m, L[23]);
+      L[24] = m2l_fma(D[42], m, L[24]);
+      L[25] = m2l_fma(D[43], m, L[25]);
+      L[26] = m2l_fma(D[45], m, L[26]);
+      L[27] = m2l_fma(D[46], m, L[27]);
+      L[28] = m2l_fma(D[47], m, L[28]);
+      L[29] = m2l_fma(D[48], m, L[29]);
+      L[30] = m2l_fma(D[50], m, L[30]);
+      L[31] = m2l_fma(D[51], m, L[31]);
+      L[32] = m2l_fma(D[52], m, L[32]);
+      L[33] = m2l_fma(D[53], m, L[33]);
+      L[34] = m2l_fma(D[54], m, L[34]);
+      L[35] = m2l_fma(D[57], m, L[35]);
+      L[36] = m2l_fma(D[59], m, L[36]);
+      L[37] = m2l_fma(D[60], m, L[37]);
+      L[38] = m2l_fma(D[62], m, L[38]);
+      L[39] = m2l_fma(D[63], m, L[39]);
+      L[40] = m2l_fma(D[64], m, L[40]);
+      L[41] = m2l_fma(D[66], m, L[41]);
+      L[42] = m2l_fma(D[67], m, L[42]);
+      L[43] = m2l_fma(D[68], m, L[43]);
+      L[44] = m2l_fma(D[69], m, L[44]);
+      L[45] = m2l_fma(D[71], m, L[45]);
+      L[46] = m2l_fma(D[72], m, L[46]);
+      L[47] = m2l_fma(D[73], m, L[47]);
+      L[48] = m2l_fma(D[74], m, L[48]);
+      L[49] = m2l_fma(D[75], m, L[49]);
+      L[50] = m2l_fma(D[77], m, L[50]);
+      L[51] = m2l_fma(D[78], m, L[51]);
+      L[52] = m2l_fma(D[79], m, L[52]);
+      L[53] = m2l_fma(D[80], m, L[53]);
+      L[54] = m2l_fma(D[81], m, L[54]);
+      L[55] = m2l_fma(D[82], m, L[55]);
     }
-    { const float m = -__ldg(Ms + 3) * rp;
-      L[1] = fmaf(D[6], m, L[1]);
-      L[2] = fmaf(D[8], m, L[2]);
-      L[3] = fmaf(D[9], m, L[3]);
-      L[4] = fmaf(D[12], m, L[4]);
-      L[5] = fmaf(D[14], m, L[5]);
-      L[6] = fmaf(D[15], m, L[6]);
-      L[7] = fmaf(D[17], m, L[7]);
-      L[8] = fmaf(D[18], m, L[8]);
-      L[9] = fmaf(D[19], m, L[9]);
-      L[10] = fmaf(D[22], m, L[10]);
-      L[11] = fmaf(D[24], m, L[11]);
-      L[12] = fmaf(D[25], m, L[12]);
-      L[13] = fmaf(D[27], m, L[13]);
-      L[14] = fmaf(D[28], m, L[14]);
-      L[15] = fmaf(D[29], m, L[15]);
-      L[16] = fmaf(D[31], m, L[16]);
-      L[17] = fmaf(D[32], m, L[17]);
-      L[18] = fmaf(D[33], m, L[18]);
-      L[19] = fmaf(D[34], m, L[19]);
-      L[20] = fmaf(D[37], m, L[20]);
-      L[21] = fmaf(D[39], m, L[21]);
-      L[22] = fmaf(D[40], m, L[22]);
-      L[23] = fmaf(D[42], m, L[23]);
-      L[24] = fmaf(D[43], m, L[24]);
-      L[25] = fmaf(D[44], m, L[25]);
-      L[26] = fmaf(D[46], m, L[26]);
-      L[27] = fmaf(D[47], m, L[27]);
-      L[28] = fmaf(D[48], m, L[28]);
-      L[29] = fmaf(D[49], m, L[29]);
-      L[30] = fmaf(D[51], m, L[30]);
-      L[31] = fmaf(D[52], m, L[31]);
-      L[32] = fmaf(D[53], m, L[32]);
-      L[33] = fmaf(D[54], m, L[33]);
-      L[34] = fmaf(D[55], m, L[34]);
-      L[35] = fmaf(D[58], m, L[35]);
-      L[36] = fmaf(D[60], m, L[36]);
-      L[37] = fmaf(D[61], m, L[37]);
-      L[38] = fmaf(D[63], m, L[38]);
-      L[39] = fmaf(D[64], m, L[39]);
-      L[40] = fmaf(D[65], m, L[40]);
-      L[41] = fmaf(D[67], m, L[41]);
-      L[42] = fmaf(D[68], m, L[42]);
-      L[43] = fmaf(D[69], m, L[43]);
-      L[44] = fmaf(D[70], m, L[44]);
-      L[45] = fmaf(D[72], m, L[45]);
-      L[46] = fmaf(D[73], m, L[46]);
-      L[47] = fmaf(D[74], m, L[47]);
-      L[48] = fmaf(D[75], m, L[48]);
-      L[49] = fmaf(D[76], m, L[49]);
-      L[50] = fmaf(D[78], m, L[50]);
-      L[51] = fmaf(D[79], m, L[51]);
-      L[52] = fmaf(D[80], m, L[52]);
-      L[53] = fmaf(D[81], m, L[53]);
-      L[54] = fmaf(D[82], m, L[54]);
-      L[55] = fmaf(D[83], m, L[55]);
-    }
-    rp *= rho;
-    { const float m = __ldg(Ms + 4) * rp;
-      L[1] = fmaf(D[10], m, L[1]);
-      L[2] = fmaf(D[11], m, L[2]);
-      L[3] = fmaf(D[12], m, L[3]);
-      L[4] = fmaf(D[20], m, L[4]);
-      L[5] = fmaf(D[21], m, L[5]);
-      L[6] = fmaf(D[22], m, L[6]);
-      L[7] = fmaf(D[23], m, L[7]);
-      L[8] = fmaf(D[24], m, L[8]);
-      L[9] = fmaf(D[25], m, L[9]);
-      L[10] = fmaf(D[35], m, L[10]);
-      L[11] = fmaf(D[36], m, L[11]);
-      L[12] = fmaf(D[37], m, L[12]);
-      L[13] = fmaf(D[38], m, L[13]);
-      L[14] = fmaf(D[39], m, L[14]);
-      L[15] = fmaf(D[40], m, L[15]);
-      L[16] = fmaf(D[41], m, L[16]);
-      L[17] = fmaf(D[42], m, L[17]);
-      L[18] = fmaf(D[43], m, L[18]);
-      L[19] = fmaf(D[44], m, L[19]);
-      L[20] = fmaf(D[56], m, L[20]);
-      L[21] = fmaf(D[57], m, L[21]);
-      L[22] = fmaf(D[58], m, L[22]);
-      L[23] = fmaf(D[59], m, L[23]);
-      L[24] = fmaf(D[60], m, L[24]);
-      L[25] = fmaf(D[61], m, L[25]);
-      L[26] = fmaf(D[62], m, L[26]);
-      L[27] = fmaf(D[63], m, L[27]);
-      L[28] = fmaf(D[64], m, L[28]);
-      L[29] = fmaf(D[65], m, L[29]);
-      L[30] = fmaf(D[66], m, L[30]);
-      L[31] = fmaf(D[67], m, L[31]);
-      L[32] = fmaf(D[68], m, L[32]);
-      L[33] = fmaf(D[69], m, L[33]);
-      L[34] = fmaf(D[70], m, L[34]);
-    }
-    { const float m = __ldg(Ms + 5) * rp;
-      L[1] = fmaf(D[11], m, L[1]);
-      L[2] = fmaf(D[13], m, L[2]);
-      L[3] = fmaf(D[14], m, L[3]);
-      L[4] = fmaf(D[21], m, L[4]);
-      L[5] = fmaf(D[23], m, L[5]);
-      L[6] = fmaf(D[24], m, L[6]);
-      L[7] = fmaf(D[26], m, L[7]);
-      L[8] = fmaf(D[27], m, L[8]);
-      L[9] = fmaf(D[28], m, L[9]);
-      L[10] = fmaf(D[36], m, L[10]);
-      L[11] = fmaf(D[38], m, L[11]);
-      L[12] = fmaf(D[39], m, L[12]);
-      L[13] = fmaf(D[41], m, L[13]);
-      L[14] = fmaf(D[42], m, L[14]);
-      L[15] = fmaf(D[43], m, L[15]);
-      L[16] = fmaf(D[45], m, L[16]);
-      L[17] = fmaf(D[46], m, L[17]);
-      L[18] = fmaf(D[47], m, L[18]);
-      L[19] = fmaf(D[48], m, L[19]);
-      L[20] = fmaf(D[57], m, L[20]);
-      L[21] = fmaf(D[59], m, L[21]);
-      L[22] = fmaf(D[60], m, L[22]);
-      L[23] = fmaf(D[62], m, L[23]);
-      L[24] = fmaf(D[63], m, L[24]);
-      L[25] = fmaf(D[64], m, L[25]);
-      L[26] = fmaf(D[66], m, L[26]);
-      L[27] = fmaf(D[67], m, L[27]);
-      L[28] = fmaf(D[68], m, L[28]);
-      L[29] = fmaf(D[69], m, L[29]);
-      L[30] = fmaf(D[71], m, L[30]);
-      L[31] = fmaf(D[72], m, L[31]);
-      L[32] = fmaf(D[73], m, L[32]);
-      L[33] = fmaf(D[74], m, L[33]);
-      L[34] = fmaf(D[75], m, L[34]);
-    }
-    { const float m = __ldg(Ms + 6) * rp;
-      L[1] = fmaf(D[12], m, L[1]);
-      L[2] = fmaf(D[14], m, L[2]);
-      L[3] = fmaf(D[15], m, L[3]);
-      L[4] = fmaf(D[22], m, L[4]);
-      L[5] = fmaf(D[24], m, L[5]);
-      L[6] = fmaf(D[25], m, L[6]);
-      L[7] = fmaf(D[27], m, L[7]);
-      L[8] = fmaf(D[28], m, L[8]);
-      L[9] = fmaf(D[29], m, L[9]);
-      L[10] = fmaf(D[37], m, L[10]);
-      L[11] = fmaf(D[39], m, L[11]);
-      L[12] = fmaf(D[40], m, L[12]);
-      L[13] = fmaf(D[42], m, L[13]);
-      L[14] = fmaf(D[43], m, L[14]);
-      L[15] = fmaf(D[44], m, L[15]);
-      L[16] = fmaf(D[46], m, L[16]);
-      L[17] = fmaf(D[47], m, L[17]);
-      L[18] = fmaf(D[48], m, L[18]);
-      L[19] = fmaf(D[49], m, L[19]);
-      L[20] = fmaf(D[58], m, L[20]);
-      L[21] = fmaf(D[60], m, L[21]);
-      L[22] = fmaf(D[61], m, L[22]);
-      L[23] = fmaf(D[63], m, L[23]);
-      L[24] = fmaf(D[64], m, L[24]);
-      L[25] = fmaf(D[65], m, L[25]);
-      L[26] = fmaf(D[67], m, L[26]);
-      L[27] = fmaf(D[68], m, L[27]);
-      L[28] = fmaf(D[69], m, L[28]);
-      L[29] = fmaf(D[70], m, L[29]);
-      L[30] = fmaf(D[72], m, L[30]);
-      L[31] = fmaf(D[73], m, L[31]);
-      L[32] = fmaf(D[74], m, L[32]);
-      L[33] = fmaf(D[75], m, L[33]);
-      L[34] = fmaf(D[76], m, L[34]);
-    }
-    { const float m = __ldg(Ms + 7) * rp;
-      L[1] = fmaf(D[13], m, L[1]);
-      L[2] = fmaf(D[16], m, L[2]);
-      L[3] = fmaf(D[17], m, L[3]);
-      L[4] = fmaf(D[23], m, L[4]);
-      L[5] = fmaf(D[26], m, L[5]);
-      L[6] = fmaf(D[27], m, L[6]);
-      L[7] = fmaf(D[30], m, L[7]);
-      L[8] = fmaf(D[31], m, L[8]);
-      L[9] = fmaf(D[32], m, L[9]);
-      L[10] = fmaf(D[38], m, L[10]);
-      L[11] = fmaf(D[41], m, L[11]);
-      L[12] = fmaf(D[42], m, L[12]);
-      L[13] = fmaf(D[45], m, L[13]);
-      L[14] = fmaf(D[46], m, L[14]);
-      L[15] = fmaf(D[47], m, L[15]);
-      L[16] = fmaf(D[50], m, L[16]);
-      L[17] = fmaf(D[51], m, L[17]);
-      L[18] = fmaf(D[52], m, L[18]);
-      L[19] = fmaf(D[53], m, L[19]);
-      L[20] = fmaf(D[59], m, L[20]);
-      L[21] = fmaf(D[62], m, L[21]);
-      L[22] = fmaf(D[63], m, L[22]);
-      L[23] = fmaf(D[66], m, L[23]);
-      L[24] = fmaf(D[67], m, L[24]);
-      L[25] = fmaf(D[68], m, L[25]);
-      L[26] = fmaf(D[71], m, L[26]);
-      L[27] = fmaf(D[72], m, L[27]);
-      L[28] = fmaf(D[73], m, L[28]);
-      L[29] = fmaf(D[74], m, L[29]);
-      L[30] = fmaf(D[77], m, L[30]);
-      L[31] = fmaf(D[78], m, L[31]);
-      L[32] = fmaf(D[79], m, L[32]);
-      L[33] = fmaf(D[80], m, L[33]);
-      L[34] = fmaf(D[81], m, L[34]);
-    }
-    { const float m = __ldg(Ms + 8) * rp;
-      L[1] = fmaf(D[14], m, L[1]);
-      L[2] = fmaf(D[17], m, L[2]);
-      L[3] = fmaf(D[18], m, L[3]);
-      L[4] = fmaf(D[24], m, L[4]);
-      L[5] = fmaf(D[27], m, L[5]);
-      L[6] = fmaf(D[28], m, L[6]);
-      L[7] = fmaf(D[31], m, L[7]);
-      L[8] = fmaf(D[32], m, L[8]);
-      L[9] = fmaf(D[33], m, L[9]);
-      L[10] = fmaf(D[39], m, L[10]);
-      L[11] = fmaf(D[42], m, L[11]);
-      L[12] = fmaf(D[43], m, L[12]);
-      L[13] = fmaf(D[46], m, L[13]);
-      L[14] = fmaf(D[47], m, L[14]);
-      L[15] = fmaf(D[48], m, L[15]);
-      L[16] = fmaf(D[51], m, L[16]);
-      L[17] = fmaf(D[52], m, L[17]);
-      L[18] = fmaf(D[53], m, L[18]);
-      L[19] = fmaf(D[54], m, L[19]);
-      L[20] = fmaf(D[60], m, L[20]);
-      L[21] = fmaf(D[63], m, L[21]);
-      L[22] = fmaf(D[64], m, L[22]);
-      L[23] = fmaf(D[67], m, L[23]);
-      L[24] = fmaf(D[68], m, L[24]);
-      L[25] = fmaf(D[69], m, L[25]);
-      L[26] = fmaf(D[72], m, L[26]);
-      L[27] = fmaf(D[73], m, L[27]);
-      L[28] = fmaf(D[74], m, L[28]);
-      L[29] = fmaf(D[75], m, L[29]);
-      L[30] = fmaf(D[78], m, L[30]);
-      L[31] = fmaf(D[79], m, L[31]);
-      L[32] = fmaf(D[80], m, L[32]);
-      L[33] = fmaf(D[81], m, L[33]);
-      L[34] = fmaf(D[82], m, L[34]);
-    }
-    { const float m = __ldg(Ms + 9) * rp;
-      L[1] = fmaf(D[15], m, L[1]);
-      L[2] = fmaf(D[18], m, L[2]);
-      L[3] = fmaf(D[19], m, L[3]);
-      L[4] = fmaf(D[25], m, L[4]);
-      L[5] = fmaf(D[28], m, L[5]);
-      L[6] = fmaf(D[29], m, L[6]);
-      L[7] = fmaf(D[32], m, L[7]);
-      L[8] = fmaf(D[33], m, L[8]);
-      L[9] = fmaf(D[34], m, L[9]);
-      L[10] = fmaf(D[40], m, L[10]);
-      L[11] = fmaf(D[43], m, L[11]);
-      L[12] = fmaf(D[44], m, L[12]);
-      L[13] = fmaf(D[47], m, L[13]);
-      L[14] = fmaf(D[48], m, L[14]);
-      L[15] = fmaf(D[49], m, L[15]);
-      L[16] = fmaf(D[52], m, L[16]);
-      L[17] = fmaf(D[53], m, L[17]);
-      L[18] = fmaf(D[54], m, L[18]);
-      L[19] = fmaf(D[55], m, L[19]);
-      L[20] = fmaf(D[61], m, L[20]);
-      L[21] = fmaf(D[64], m, L[21]);
-      L[22] = fmaf(D[65], m, L[22]);
-      L[23] = fmaf(D[68], m, L[23]);
-      L[24] = fmaf(D[69], m, L[24]);
-      L[25] = fmaf(D[70], m, L[25]);
-      L[26] = fmaf(D[73], m, L[26]);
-      L[27] = fmaf(D[74], m, L[27]);
-      L[28] = fmaf(D[75], m, L[28]);
-      L[29] = fmaf(D[76], m, L[29]);
-      L[30] = fmaf(D[79], m, L[30]);
-      L[31] = fmaf(D[80], m, L[31]);
-      L[32] = fmaf(D[81], m, L[32]);
-      L[33] = fmaf(D[82], m, L[33]);
-      L[34] = fmaf(D[83], m, L[34]);
+    { const T m = -__ldg(Ms + 3) * rp;
+      L[1] = m2l_fma(D[6], m, L[1]);
+      L[2] = m2l_fma(D[8], m, L[2]);
+      L[3] = m2l_fma(D[9], m, L[3]);
+      L[4] = m2l_fma(D[12], m, L[4]);
+      L[5] = m2l_fma(D[14], m, L[5]);
+      L[6] = m2l_fma(D[15], m, L[6]);
+      L[7] = m2l_fma(D[17], m, L[7]);
+      L[8] = m2l_fma(D[18], m, L[8]);
+      L[9] = m2l_fma(D[19], m, L[9]);
+      L[10] = m2l_fma(D[22], m, L[10]);
+      L[11] = m2l_fma(D[24], m, L[11]);
+      L[12] = m2l_fma(D[25], m, L[12]);
+      L[13] = m2l_fma(D[27], m, L[13]);
+      L[14] = m2l_fma(D[28], m, L[14]);
+      L[15] = m2l_fma(D[29], m, L[15]);
+      L[16] = m2l_fma(D[31], m, L[16]);
+      L[17] = m2l_fma(D[32], m, L[17]);
+      L[18] = m2l_fma(D[33], m, L[18]);
+      L[19] = m2l_fma(D[34], m, L[19]);
+      L[20] = m2l_fma(D[37], m, L[20]);
+      L[21] = m2l_fma(D[39], m, L[21]);
+      L[22] = m2l_fma(D[40], m, L[22]);
+      L[23] = m2l_fma(D[42], m, L[23]);
+      L[24] = m2l_fma(D[43], m, L[24]);
+      L[25] = m2l_fma(D[44], m, L[25]);
+      L[26] = m2l_fma(D[46], m, L[26]);
+      L[27] = m2l_fma(D[47], m, L[27]);
+      L[28] = m2l_fma(D[48], m, L[28]);
+      L[29] = m2l_fma(D[49], m, L[29]);
+      L[30] = m2l_fma(D[51], m, L[30]);
+      L[31] = m2l_fma(D[52], m, L[31]);
+      L[32] = m2l_fma(D[53], m, L[32]);
+      L[33] = m2l_fma(D[54], m, L[33]);
+      L[34] = m2l_fma(D[55], m, L[34]);
+      L[35] = m2l_fma(D[58], m, L[35]);
+      L[36] = m2l_fma(D[60], m, L[36]);
+      L[37] = m2l_fma(D[61], m, L[37]);
+      L[38] = m2l_fma(D[63], m, L[38]);
+      L[39] = m2l_fma(D[64], m, L[39]);
+      L[40] = m2l_fma(D[65], m, L[40]);
+      L[41] = m2l_fma(D[67], m, L[41]);
+      L[42] = m2l_fma(D[68], m, L[42]);
+      L[43] = m2l_fma(D[69], m, L[43]);
+      L[44] = m2l_fma(D[70], m, L[44]);
+      L[45] = m2l_fma(D[72], m, L[45]);
+      L[46] = m2l_fma(D[73], m, L[46]);
+      L[47] = m2l_fma(D[74], m, L[47]);
+      L[48] = m2l_fma(D[75], m, L[48]);
+      L[49] = m2l_fma(D[76], m, L[49]);
+      L[50] = m2l_fma(D[78], m, L[50]);
+      L[51] = m2l_fma(D[79], m, L[51]);
+      L[52] = m2l_fma(D[80], m, L[52]);
+      L[53] = m2l_fma(D[81], m, L[53]);
+      L[54] = m2l_fma(D[82], m, L[54]);
+      L[55] = m2l_fma(D[83], m, L[55]);
     }
     rp *= rho;
-    { const float m = -__ldg(Ms + 10) * rp;
-      L[1] = fmaf(D[20], m, L[1]);
-      L[2] = fmaf(D[21], m, L[2]);
-      L[3] = fmaf(D[22], m, L[3]);
-      L[4] = fmaf(D[35], m, L[4]);
-      L[5] = fmaf(D[36], m, L[5]);
-      L[6] = fmaf(D[37], m, L[6]);
-      L[7] = fmaf(D[38], m, L[7]);
-      L[8] = fmaf(D[39], m, L[8]);
-      L[9] = fmaf(D[40], m, L[9]);
-      L[10] = fmaf(D[56], m, L[10]);
-      L[11] = fmaf(D[57], m, L[11]);
-      L[12] = fmaf(D[58], m, L[12]);
-      L[13] = fmaf(D[59], m, L[13]);
-      L[14] = fmaf(D[60], m, L[14]);
-      L[15] = fmaf(D[61], m, L[15]);
-      L[16] = fmaf(D[62], m, L[16]);
-      L[17] = fmaf(D[63], m, L[17]);
-      L[18] = fmaf(D[64], m, L[18]);
-      L[19] = fmaf(D[65], m, L[19]);
+    { const T m = __ldg(Ms + 4) * rp;
+      L[1] = m2l_fma(D[10], m, L[1]);
+      L[2] = m2l_fma(D[11], m, L[2]);
+      L[3] = m2l_fma(D[12], m, L[3]);
+      L[4] = m2l_fma(D[20], m, L[4]);
+      L[5] = m2l_fma(D[21], m, L[5]);
+      L[6] = m2l_fma(D[22], m, L[6]);
+      L[7] = m2l_fma(D[23], m, L[7]);
+      L[8] = m2l_fma(D[24], m, L[8]);
+      L[9] = m2l_fma(D[25], m, L[9]);
+      L[10] = m2l_fma(D[35], m, L[10]);
+      L[11] = m2l_fma(D[36], m, L[11]);
+      L[12] = m2l_fma(D[37], m, L[12]);
+      L[13] = m2l_fma(D[38], m, L[13]);
+      L[14] = m2l_fma(D[39], m, L[14]);
+      L[15] = m2l_fma(D[40], m, L[15]);
+      L[16] = m2l_fma(D[41], m, L[16]);
+      L[17] = m2l_fma(D[42], m, L[17]);
+      L[18] = m2l_fma(D[43], m, L[18]);
+      L[19] = m2l_fma(D[44], m, L[19]);
+      L[20] = m2l_fma(D[56], m, L[20]);
+      L[21] = m2l_fma(D[57], m, L[21]);
+      L[22] = m2l_fma(D[58], m, L[22]);
+      L[23] = m2l_fma(D[59], m, L[23]);
+      L[24] = m2l_fma(D[60], m, L[24]);
+      L[25] = m2l_fma(D[61], m, L[25]);
+      L[26] = m2l_fma(D[62], m, L[26]);
+      L[27] = m2l_fma(D[63], m, L[27]);
+      L[28] = m2l_fma(D[64], m, L[28]);
+      L[29] = m2l_fma(D[65], m, L[29]);
+      L[30] = m2l_fma(D[66], m, L[30]);
+      L[31] = m2l_fma(D[67], m, L[31]);
+      L[32] = m2l_fma(D[68], m, L[32]);
+      L[33] = m2l_fma(D[69], m, L[33]);
+      L[34] = m2l_fma(D[70], m, L[34]);
     }
-    { const float m = -__ldg(Ms + 11) * rp;
-      L[1] = fmaf(D[21], m, L[1]);
-      L[2] = fmaf(D[23], m, L[2]);
-      L[3] = fmaf(D[24], m, L[3]);
-      L[4] = fmaf(D[36], m, L[4]);
-      L[5] = fmaf(D[38], m, L[5]);
-      L[6] = fmaf(D[39], m, L[6]);
-      L[7] = fmaf(D[41], m, L[7]);
-      L[8] = fmaf(D[42], m, L[8]);
-      L[9] = fmaf(D[43], m, L[9]);
-      L[10] = fmaf(D[57], m, L[10]);
-      L[11] = fmaf(D[59], m, L[11]);
-      L[12] = fmaf(D[60], m, L[12]);
-      L[13] = fmaf(D[62], m, L[13]);
-      L[14] = fmaf(D[63], m, L[14]);
-      L[15] = fmaf(D[64], m, L[15]);
-      L[16] = fmaf(D[66], m, L[16]);
-      L[17] = fmaf(D[67], m, L[17]);
-      L[18] = fmaf(D[68], m, L[18]);
-      L[19] = fmaf(D[69], m, L[19]);
+    { const T m = __ldg(Ms + 5) * rp;
+      L[1] = m2l_fma(D[11], m, L[1]);
+      L[2] = m2l_fma(D[13], m, L[2]);
+      L[3] = m2l_fma(D[14], m, L[3]);
+      L[4] = m2l_fma(D[21], m, L[4]);
+      L[5] = m2l_fma(D[23], m, L[5]);
+      L[6] = m2l_fma(D[24], m, L[6]);
+      L[7] = m2l_fma(D[26], m, L[7]);
+      L[8] = m2l_fma(D[27], m, L[8]);
+      L[9] = m2l_fma(D[28], m, L[9]);
+      L[10] = m2l_fma(D[36], m, L[10]);
+      L[11] = m2l_fma(D[38], m, L[11]);
+      L[12] = m2l_fma(D[39], m, L[12]);
+      L[13] = m2l_fma(D[41], m, L[13]);
+      L[14] = m2l_fma(D[42], m, L[14]);
+      L[15] = m2l_fma(D[43], m, L[15]);
+      L[16] = m2l_fma(D[45], m, L[16]);
+      L[17] = m2l_fma(D[46], m, L[17]);
+      L[18] = m2l_fma(D[47], m, L[18]);
+      L[19] = m2l_fma(D[48], m, L[19]);
+      L[20] = m2l_fma(D[57], m, L[20]);
+      L[21] = m2l_fma(D[59], m, L[21]);
+      L[22] = m2l_fma(D[60], m, L[22]);
+      L[23] = m2l_fma(D[62], m, L[23]);
+      L[24] = m2l_fma(D[63], m, L[24]);
+      L[25] = m2l_fma(D[64], m, L[25]);
+      L[26] = m2l_fma(D[66], m, L[26]);
+      L[27] = m2l_fma(D[67], m, L[27]);
+      L[28] = m2l_fma(D[68], m, L[28]);
+      L[29] = m2l_fma(D[69], m, L[29]);
+      L[30] = m2l_fma(D[71], m, L[30]);
+      L[31] = m2l_fma(D[72], m, L[31]);
+      L[32] = m2l_fma(D[73], m, L[32]);
+      L[33] = m2l_fma(D[74], m, L[33]);
+      L[34] = m2l_fma(D[75], m, L[34]);
     }
-    { const float m = -__ldg(Ms + 12) * rp;
-      L[1] = fmaf(D[22], m, L[1]);
-      L[2] = fmaf(D[24], m, L[2]);
-      L[3] = fmaf(D[25], m, L[3]);
-      L[4] = fmaf(D[37], m, L[4]);
-      L[5] = fmaf(D[39], m, L[5]);
-      L[6] = fmaf(D[40], m, L[6]);
-      L[7] = fmaf(D[42], m, L[7]);
-      L[8] = fmaf(D[43], m, L[8]);
-      L[9] = fmaf(D[44], m, L[9]);
-      L[10] = fmaf(D[58], m, L[10]);
-      L[11] = fmaf(D[60], m, L[11]);
-      L[12] = fmaf(D[61], m, L[12]);
-      L[13] = fmaf(D[63], m, L[13]);
-      L[14] = fmaf(D[64], m, L[14]);
-      L[15] = fmaf(D[65], m, L[15]);
-      L[16] = fmaf(D[67], m, L[16]);
-      L[17] = fmaf(D[68], m, L[17]);
-      L[18] = fmaf(D[69], m, L[18]);
-      L[19] = fmaf(D[70], m, L[19]);
+    { const T m = __ldg(Ms + 6) * rp;
+      L[1] = m2l_fma(D[12], m, L[1]);
+      L[2] = m2l_fma(D[14], m, L[2]);
+      L[3] = m2l_fma(D[15], m, L[3]);
+      L[4] = m2l_fma(D[22], m, L[4]);
+      L[5] = m2l_fma(D[24], m, L[5]);
+      L[6] = m2l_fma(D[25], m, L[6]);
+      L[7] = m2l_fma(D[27], m, L[7]);
+      L[8] = m2l_fma(D[28], m, L[8]);
+      L[9] = m2l_fma(D[29], m, L[9]);
+      L[10] = m2l_fma(D[37], m, L[10]);
+      L[11] = m2l_fma(D[39], m, L[11]);
+      L[12] = m2l_fma(D[40], m, L[12]);
+      L[13] = m2l_fma(D[42], m, L[13]);
+      L[14] = m2l_fma(D[43], m, L[14]);
+      L[15] = m2l_fma(D[44], m, L[15]);
+      L[16] = m2l_fma(D[46], m, L[16]);
+      L[17] = m2l_fma(D[47], m, L[17]);
+      L[18] = m2l_fma(D[48], m, L[18]);
+      L[19] = m2l_fma(D[49], m, L[19]);
+      L[20] = m2l_fma(D[58], m, L[20]);
+      L[21] = m2l_fma(D[60], m, L[21]);
+      L[22] = m2l_fma(D[61], m, L[22]);
+      L[23] = m2l_fma(D[63], m, L[23]);
+      L[24] = m2l_fma(D[64], m, L[24]);
+      L[25] = m2l_fma(D[65], m, L[25]);
+      L[26] = m2l_fma(D[67], m, L[26]);
+      L[27] = m2l_fma(D[68], m, L[27]);
+      L[28] = m2l_fma(D[69], m, L[28]);
+      L[29] = m2l_fma(D[70], m, L[29]);
+      L[30] = m2l_fma(D[72], m, L[30]);
+      L[31] = m2l_fma(D[73], m, L[31]);
+      L[32] = m2l_fma(D[74], m, L[32]);
+      L[33] = m2l_fma(D[75], m, L[33]);
+      L[34] = m2l_fma(D[76], m, L[34]);
     }
-    { const float m = -__ldg(Ms + 13) * rp;
-      L[1] = fmaf(D[23], m, L[1]);
-      L[2] = fmaf(D[26], m, L[2]);
-      L[3] = fmaf(D[27], m, L[3]);
-      L[4] = fmaf(D[38], m, L[4]);
-      L[5] = fmaf(D[41], m, L[5]);
-      L[6] = fmaf(D[42], m, L[6]);
-      L[7] = fmaf(D[45], m, L[7]);
-      L[8] = fmaf(D[46], m, L[8]);
-      L[9] = fmaf(D[47], m, L[9]);
-      L[10] = fmaf(D[59], m, L[10]);
-      L[11] = fmaf(D[62], m, L[11]);
-      L[12] = fmaf(D[63], m, L[12]);
-      L[13] = fmaf(D[66], m, L[13]);
-      L[14] = fmaf(D[67], m, L[14]);
-      L[15] = fmaf(D[68], m, L[15]);
-      L[16] = fmaf(D[71], m, L[16]);
-      L[17] = fmaf(D[72], m, L[17]);
-      L[18] = fmaf(D[73], m, L[18]);
-      L[19] = fmaf(D[74], m, L[19]);
+    { const T m = __ldg(Ms + 7) * rp;
+      L[1] = m2l_fma(D[13], m, L[1]);
+      L[2] = m2l_fma(D[16], m, L[2]);
+      L[3] = m2l_fma(D[17], m, L[3]);
+      L[4] = m2l_fma(D[23], m, L[4]);
+      L[5] = m2l_fma(D[26], m, L[5]);
+      L[6] = m2l_fma(D[27], m, L[6]);
+      L[7] = m2l_fma(D[30], m, L[7]);
+      L[8] = m2l_fma(D[31], m, L[8]);
+      L[9] = m2l_fma(D[32], m, L[9]);
+      L[10] = m2l_fma(D[38], m, L[10]);
+      L[11] = m2l_fma(D[41], m, L[11]);
+      L[12] = m2l_fma(D[42], m, L[12]);
+      L[13] = m2l_fma(D[45], m, L[13]);
+      L[14] = m2l_fma(D[46], m, L[14]);
+      L[15] = m2l_fma(D[47], m, L[15]);
+      L[16] = m2l_fma(D[50], m, L[16]);
+      L[17] = m2l_fma(D[51], m, L[17]);
+      L[18] = m2l_fma(D[52], m, L[18]);
+      L[19] = m2l_fma(D[53], m, L[19]);
+      L[20] = m2l_fma(D[59], m, L[20]);
+      L[21] = m2l_fma(D[62], m, L[21]);
+      L[22] = m2l_fma(D[63], m, L[22]);
+      L[23] = m2l_fma(D[66], m, L[23]);
+      L[24] = m2l_fma(D[67], m, L[24]);
+      L[25] = m2l_fma(D[68], m, L[25]);
+      L[26] = m2l_fma(D[71], m, L[26]);
+      L[27] = m2l_fma(D[72], m, L[27]);
+      L[28] = m2l_fma(D[73], m, L[28]);
+      L[29] = m2l_fma(D[74], m, L[29]);
+      L[30] = m2l_fma(D[77], m, L[30]);
+      L[31] = m2l_fma(D[78], m, L[31]);
+      L[32] = m2l_fma(D[79], m, L[32]);
+      L[33] = m2l_fma(D[80], m, L[33]);
+      L[34] = m2l_fma(D[81], m, L[34]);
     }
-    { const float m = -__ldg(Ms + 14) * rp;
-      L[1] = fmaf(D[24], m, L[1]);
-      L[2] = fmaf(D[27], m, L[2]);
-      L[3] = fmaf(D[28], m, L[3]);
-      L[4] = fmaf(D[39], m, L[4]);
-      L[5] = fmaf(D[42], m, L[5]);
-      L[6] = fmaf(D[43], m, L[6]);
-      L[7] = fmaf(D[46], m, L[7]);
-      L[8] = fmaf(D[47], m, L[8]);
-      L[9] = fmaf(D[48], m, L[9]);
-      L[10] = fmaf(D[60], m, L[10]);
-      L[11] = fmaf(D[63], m, L[11]);
-      L[12] = fmaf(D[64], m, L[12]);
-      L[13] = fmaf(D[67], m, L[13]);
-      L[14] = fmaf(D[68], m, L[14]);
-      L[15] = fmaf(D[69], m, L[15]);
-      L[16] = fmaf(D[72], m, L[16]);
-      L[17] = fmaf(D[73], m, L[17]);
-      L[18] = fmaf(D[74], m, L[18]);
-      L[19] = fmaf(D[75], m, L[19]);
+    { const T m = __ldg(Ms + 8) * rp;
+      L[1] = m2l_fma(D[14], m, L[1]);
+      L[2] = m2l_fma(D[17], m, L[2]);
+      L[3] = m2l_fma(D[18], m, L[3]);
+      L[4] = m2l_fma(D[24], m, L[4]);
+      L[5] = m2l_fma(D[27], m, L[5]);
+      L[6] = m2l_fma(D[28], m, L[6]);
+      L[7] = m2l_fma(D[31], m, L[7]);
+      L[8] = m2l_fma(D[32], m, L[8]);
+      L[9] = m2l_fma(D[33], m, L[9]);
+      L[10] = m2l_fma(D[39], m, L[10]);
+      L[11] = m2l_fma(D[42], m, L[11]);
+      L[12] = m2l_fma(D[43], m, L[12]);
+      L[13] = m2l_fma(D[46], m, L[13]);
+      L[14] = m2l_fma(D[47], m, L[14]);
+      L[15] = m2l_fma(D[48], m, L[15]);
+      L[16] = m2l_fma(D[51], m, L[16]);
+      L[17] = m2l_fma(D[52], m, L[17]);
+      L[18] = m2l_fma(D[53], m, L[18]);
+      L[19] = m2l_fma(D[54], m, L[19]);
+      L[20] = m2l_fma(D[60], m, L[20]);
+      L[21] = m2l_fma(D[63], m, L[21]);
+      L[22] = m2l_fma(D[64], m, L[22]);
+      L[23] = m2l_fma(D[67], m, L[23]);
+      L[24] = m2l_fma(D[68], m, L[24]);
+      L[25] = m2l_fma(D[69], m, L[25]);
+      L[26] = m2l_fma(D[72], m, L[26]);
+      L[27] = m2l_fma(D[73], m, L[27]);
+      L[28] = m2l_fma(D[74], m, L[28]);
+      L[29] = m2l_fma(D[75], m, L[29]);
+      L[30] = m2l_fma(D[78], m, L[30]);
+      L[31] = m2l_fma(D[79], m, L[31]);
+      L[32] = m2l_fma(D[80], m, L[32]);
+      L[33] = m2l_fma(D[81], m, L[33]);
+      L[34] = m2l_fma(D[82], m, L[34]);
     }
-    { const float m = -__ldg(Ms + 15) * rp;
-      L[1] = fmaf(D[25], m, L[1]);
-      L[2] = fmaf(D[28], m, L[2]);
-      L[3] = fmaf(D[29], m, L[3]);
-      L[4] = fmaf(D[40], m, L[4]);
-      L[5] = fmaf(D[43], m, L[5]);
-      L[6] = fmaf(D[44], m, L[6]);
-      L[7] = fmaf(D[47], m, L[7]);
-      L[8] = fmaf(D[48], m, L[8]);
-      L[9] = fmaf(D[49], m, L[9]);
-      L[10] = fmaf(D[61], m, L[10]);
-      L[11] = fmaf(D[64], m, L[11]);
-      L[12] = fmaf(D[65], m, L[12]);
-      L[13] = fmaf(D[68], m, L[13]);
-      L[14] = fmaf(D[69], m, L[14]);
-      L[15] = fmaf(D[70], m, L[15]);
-      L[16] = fmaf(D[73], m, L[16]);
-      L[17] = fmaf(D[74], m, L[17]);
-      L[18] = fmaf(D[75], m, L[18]);
-      L[19] = fmaf(D[76], m, L[19]);
-    }
-    { const float m = -__ldg(Ms + 16) * rp;
-      L[1] = fmaf(D[26], m, L[1]);
-      L[2] = fmaf(D[30], m, L[2]);
-      L[3] = fmaf(D[31], m, L[3]);
-      L[4] = fmaf(D[41], m, L[4]);
-      L[5] = fmaf(D[45], m, L[5]);
-      L[6] = fmaf(D[46], m, L[6]);
-      L[7] = fmaf(D[50], m, L[7]);
-      L[8] = fmaf(D[51], m, L[8]);
-      L[9] = fmaf(D[52], m, L[9]);
-      L[10] = fmaf(D[62], m, L[10]);
-      L[11] = fmaf(D[66], m, L[11]);
-      L[12] = fmaf(D[67], m, L[12]);
-      L[13] = fmaf(D[71], m, L[13]);
-      L[14] = fmaf(D[72], m, L[14]);
-      L[15] = fmaf(D[73], m, L[15]);
-      L[16] = fmaf(D[77], m, L[16]);
-      L[17] = fmaf(D[78], m, L[17]);
-      L[18] = fmaf(D[79], m, L[18]);
-      L[19] = fmaf(D[80], m, L[19]);
-    }
-    { const float m = -__ldg(Ms + 17) * rp;
-      L[1] = fmaf(D[27], m, L[1]);
-      L[2] = fmaf(D[31], m, L[2]);
-      L[3] = fmaf(D[32], m, L[3]);
-      L[4] = fmaf(D[42], m, L[4]);
-      L[5] = fmaf(D[46], m, L[5]);
-      L[6] = fmaf(D[47], m, L[6]);
-      L[7] = fmaf(D[51], m, L[7]);
-      L[8] = fmaf(D[52], m, L[8]);
-      L[9] = fmaf(D[53], m, L[9]);
-      L[10] = fmaf(D[63], m, L[10]);
-      L[11] = fmaf(D[67], m, L[11]);
-      L[12] = fmaf(D[68], m, L[12]);
-      L[13] = fmaf(D[72], m, L[13]);
-      L[14] = fmaf(D[73], m, L[14]);
-      L[15] = fmaf(D[74], m, L[15]);
-      L[16] = fmaf(D[78], m, L[16]);
-      L[17] = fmaf(D[79], m, L[17]);
-      L[18] = fmaf(D[80], m, L[18]);
-      L[19] = fmaf(D[81], m, L[19]);
-    }
-    { const float m = -__ldg(Ms + 18) * rp;
-      L[1] = fmaf(D[28], m, L[1]);
-      L[2] = fmaf(D[32], m, L[2]);
-      L[3] = fmaf(D[33], m, L[3]);
-      L[4] = fmaf(D[43], m, L[4]);
-      L[5] = fmaf(D[47], m, L[5]);
-      L[6] = fmaf(D[48], m, L[6]);
-      L[7] = fmaf(D[52], m, L[7]);
-      L[8] = fmaf(D[53], m, L[8]);
-      L[9] = fmaf(D[54], m, L[9]);
-      L[10] = fmaf(D[64], m, L[10]);
-      L[11] = fmaf(D[68], m, L[11]);
-      L[12] = fmaf(D[69], m, L[12]);
-      L[13] = fmaf(D[73], m, L[13]);
-      L[14] = fmaf(D[74], m, L[14]);
-      L[15] = fmaf(D[75], m, L[15]);
-      L[16] = fmaf(D[79], m, L[16]);
-      L[17] = fmaf(D[80], m, L[17]);
-      L[18] = fmaf(D[81], m, L[18]);
-      L[19] = fmaf(D[82], m, L[19]);
-    }
-    { const float m = -__ldg(Ms + 19) * rp;
-      L[1] = fmaf(D[29], m, L[1]);
-      L[2] = fmaf(D[33], m, L[2]);
-      L[3] = fmaf(D[34], m, L[3]);
-      L[4] = fmaf(D[44], m, L[4]);
-      L[5] = fmaf(D[48], m, L[5]);
-      L[6] = fmaf(D[49], m, L[6]);
-      L[7] = fmaf(D[53], m, L[7]);
-      L[8] = fmaf(D[54], m, L[8]);
-      L[9] = fmaf(D[55], m, L[9]);
-      L[10] = fmaf(D[65], m, L[10]);
-      L[11] = fmaf(D[69], m, L[11]);
-      L[12] = fmaf(D[70], m, L[12]);
-      L[13] = fmaf(D[74], m, L[13]);
-      L[14] = fmaf(D[75], m, L[14]);
-      L[15] = fmaf(D[76], m, L[15]);
-      L[16] = fmaf(D[80], m, L[16]);
-      L[17] = fmaf(D[81], m, L[17]);
-      L[18] = fmaf(D[82], m, L[18]);
-      L[19] = fmaf(D[83], m, L[19]);
-    }
-    rp *= rho;
-    { const float m = __ldg(Ms + 20) * rp;
-      L[1] = fmaf(D[35], m, L[1]);
-      L[2] = fmaf(D[36], m, L[2]);
-      L[3] = fmaf(D[37], m, L[3]);
-      L[4] = fmaf(D[56], m, L[4]);
-      L[5] = fmaf(D[57], m, L[5]);
-      L[6] = fmaf(D[58], m, L[6]);
-      L[7] = fmaf(D[59], m, L[7]);
-      L[8] = fmaf(D[60], m, L[8]);
-      L[9] = fmaf(D[61], m, L[9]);
-    }
-    { const float m = __ldg(Ms + 21) * rp;
-      L[1] = fmaf(D[36], m, L[1]);
-      L[2] = fmaf(D[38], m, L[2]);
-      L[3] = fmaf(D[39], m, L[3]);
-      L[4] = fmaf(D[57], m, L[4]);
-      L[5] = fmaf(D[59], m, L[5]);
-      L[6] = fmaf(D[60], m, L[6]);
-      L[7] = fmaf(D[62], m, L[7]);
-      L[8] = fmaf(D[63], m, L[8]);
-      L[9] = fmaf(D[64], m, L[9]);
-    }
-    { const float m = __ldg(Ms + 22) * rp;
-      L[1] = fmaf(D[37], m, L[1]);
-      L[2] = fmaf(D[39], m, L[2]);
-      L[3] = fmaf(D[40], m, L[3]);
-      L[4] = fmaf(D[58], m, L[4]);
-      L[5] = fmaf(D[60], m, L[5]);
-      L[6] = fmaf(D[61], m, L[6]);
-      L[7] = fmaf(D[63], m, L[7]);
-      L[8] = fmaf(D[64], m, L[8]);
-      L[9] = fmaf(D[65], m, L[9]);
-    }
-    { const float m = __ldg(Ms + 23) * rp;
-      L[1] = fmaf(D[38], m, L[1]);
-      L[2] = fmaf(D[41], m, L[2]);
-      L[3] = fmaf(D[42], m, L[3]);
-      L[4] = fmaf(D[59], m, L[4]);
-      L[5] = fmaf(D[62], m, L[5]);
-      L[6] = fmaf(D[63], m, L[6]);
-      L[7] = fmaf(D[66], m, L[7]);
-      L[8] = fmaf(D[67], m, L[8]);
-      L[9] = fmaf(D[68], m, L[9]);
-    }
-    { const float m = __ldg(Ms + 24) * rp;
-      L[1] = fmaf(D[39], m, L[1]);
-      L[2] = fmaf(D[42], m, L[2]);
-      L[3] = fmaf(D[43], m, L[3]);
-      L[4] = fmaf(D[60], m, L[4]);
-      L[5] = fmaf(D[63], m, L[5]);
-      L[6] = fmaf(D[64], m, L[6]);
-      L[7] = fmaf(D[67], m, L[7]);
-      L[8] = fmaf(D[68], m, L[8]);
-      L[9] = fmaf(D[69], m, L[9]);
-    }
-    { const float m = __ldg(Ms + 25) * rp;
-      L[1] = fmaf(D[40], m, L[1]);
-      L[2] = fmaf(D[43], m, L[2]);
-      L[3] = fmaf(D[44], m, L[3]);
-      L[4] = fmaf(D[61], m, L[4]);
-      L[5] = fmaf(D[64], m, L[5]);
-      L[6] = fmaf(D[65], m, L[6]);
-      L[7] = fmaf(D[68], m, L[7]);
-      L[8] = fmaf(D[69], m, L[8]);
-      L[9] = fmaf(D[70], m, L[9]);
-    }
-    { const float m = __ldg(Ms + 26) * rp;
-      L[1] = fmaf(D[41], m, L[1]);
-      L[2] = fmaf(D[45], m, L[2]);
-      L[3] = fmaf(D[46], m, L[3]);
-      L[4] = fmaf(D[62], m, L[4]);
-      L[5] = fmaf(D[66], m, L[5]);
-      L[6] = fmaf(D[67], m, L[6]);
-      L[7] = fmaf(D[71], m, L[7]);
-      L[8] = fmaf(D[72], m, L[8]);
-      L[9] = fmaf(D[73], m, L[9]);
-    }
-    { const float m = __ldg(Ms + 27) * rp;
-      L[1] = fmaf(D[42], m, L[1]);
-      L[2] = fmaf(D[46], m, L[2]);
-      L[3] = fmaf(D[47], m, L[3]);
-      L[4] = fmaf(D[63], m, L[4]);
-      L[5] = fmaf(D[67], m, L[5]);
-      L[6] = fmaf(D[68], m, L[6]);
-      L[7] = fmaf(D[72], m, L[7]);
-      L[8] = fmaf(D[73], m, L[8]);
-      L[9] = fmaf(D[74], m, L[9]);
-    }
-    { const float m = __ldg(Ms + 28) * rp;
-      L[1] = fmaf(D[43], m, L[1]);
-      L[2] = fmaf(D[47], m, L[2]);
-      L[3] = fmaf(D[48], m, L[3]);
-      L[4] = fmaf(D[64], m, L[4]);
-      L[5] = fmaf(D[68], m, L[5]);
-      L[6] = fmaf(D[69], m, L[6]);
-      L[7] = fmaf(D[73], m, L[7]);
-      L[8] = fmaf(D[74], m, L[8]);
-      L[9] = fmaf(D[75], m, L[9]);
-    }
-    { const float m = __ldg(Ms + 29) * rp;
-      L[1] = fmaf(D[44], m, L[1]);
-      L[2] = fmaf(D[48], m, L[2]);
-      L[3] = fmaf(D[49], m, L[3]);
-      L[4] = fmaf(D[65], m, L[4]);
-      L[5] = fmaf(D[69], m, L[5]);
-      L[6] = fmaf(D[70], m, L[6]);
-      L[7] = fmaf(D[74], m, L[7]);
-      L[8] = fmaf(D[75], m, L[8]);
-      L[9] = fmaf(D[76], m, L[9]);
-    }
-    { const float m = __ldg(Ms + 30) * rp;
-      L[1] = fmaf(D[45], m, L[1]);
-      L[2] = fmaf(D[50], m, L[2]);
-      L[3] = fmaf(D[51], m, L[3]);
-      L[4] = fmaf(D[66], m, L[4]);
-      L[5] = fmaf(D[71], m, L[5]);
-      L[6] = fmaf(D[72], m, L[6]);
-      L[7] = fmaf(D[77], m, L[7]);
-      L[8] = fmaf(D[78], m, L[8]);
-      L[9] = fmaf(D[79], m, L[9]);
-    }
-    { const float m = __ldg(Ms + 31) * rp;
-      L[1] = fmaf(D[46], m, L[1]);
-      L[2] = fmaf(D[51], m, L[2]);
-      L[3] = fmaf(D[52], m, L[3]);
-      L[4] = fmaf(D[67], m, L[4]);
-      L[5] = fmaf(D[72], m, L[5]);
-      L[6] = fmaf(D[73], m, L[6]);
-      L[7] = fmaf(D[78], m, L[7]);
-      L[8] = fmaf(D[79], m, L[8]);
-      L[9] = fmaf(D[80], m, L[9]);
-    }
-    { const float m = __ldg(Ms + 32) * rp;
-      L[1] = fmaf(D[47], m, L[1]);
-      L[2] = fmaf(D[52], m, L[2]);
-      L[3] = fmaf(D[53], m, L[3]);
-      L[4] = fmaf(D[68], m, L[4]);
-      L[5] = fmaf(D[73], m, L[5]);
-      L[6] = fmaf(D[74], m, L[6]);
-      L[7] = fmaf(D[79], m, L[7]);
-      L[8] = fmaf(D[80], m, L[8]);
-      L[9] = fmaf(D[81], m, L[9]);
-    }
-    { const float m = __ldg(Ms + 33) * rp;
-      L[1] = fmaf(D[48], m, L[1]);
-      L[2] = fmaf(D[53], m, L[2]);
-      L[3] = fmaf(D[54], m, L[3]);
-      L[4] = fmaf(D[69], m, L[4]);
-      L[5] = fmaf(D[74], m, L[5]);
-      L[6] = fmaf(D[75], m, L[6]);
-      L[7] = fmaf(D[80], m, L[7]);
-      L[8] = fmaf(D[81], m, L[8]);
-      L[9] = fmaf(D[82], m, L[9]);
-    }
-    { const float m = __ldg(Ms + 34) * rp;
-      L[1] = fmaf(D[49], m, L[1]);
-      L[2] = fmaf(D[54], m, L[2]);
-      L[3] = fmaf(D[55], m, L[3]);
-      L[4] = fmaf(D[70], m, L[4]);
-      L[5] = fmaf(D[75], m, L[5]);
-      L[6] = fmaf(D[76], m, L[6]);
-      L[7] = fmaf(D[81], m, L[7]);
-      L[8] = fmaf(D[82], m, L[8]);
-      L[9] = fmaf(D[83], m, L[9]);
+    { const T m = __ldg(Ms + 9) * rp;
+      L[1] = m2l_fma(D[15], m, L[1]);
+      L[2] = m2l_fma(D[18], m, L[2]);
+      L[3] = m2l_fma(D[19], m, L[3]);
+      L[4] = m2l_fma(D[25], m, L[4]);
+      L[5] = m2l_fma(D[28], m, L[5]);
+      L[6] = m2l_fma(D[29], m, L[6]);
+      L[7] = m2l_fma(D[32], m, L[7]);
+      L[8] = m2l_fma(D[33], m, L[8]);
+      L[9] = m2l_fma(D[34], m, L[9]);
+      L[10] = m2l_fma(D[40], m, L[10]);
+      L[11] = m2l_fma(D[43], m, L[11]);
+      L[12] = m2l_fma(D[44], m, L[12]);
+      L[13] = m2l_fma(D[47], m, L[13]);
+      L[14] = m2l_fma(D[48], m, L[14]);
+      L[15] = m2l_fma(D[49], m, L[15]);
+      L[16] = m2l_fma(D[52], m, L[16]);
+      L[17] = m2l_fma(D[53], m, L[17]);
+      L[18] = m2l_fma(D[54], m, L[18]);
+      L[19] = m2l_fma(D[55], m, L[19]);
+      L[20] = m2l_fma(D[61], m, L[20]);
+      L[21] = m2l_fma(D[64], m, L[21]);
+      L[22] = m2l_fma(D[65], m, L[22]);
+      L[23] = m2l_fma(D[68], m, L[23]);
+      L[24] = m2l_fma(D[69], m, L[24]);
+      L[25] = m2l_fma(D[70], m, L[25]);
+      L[26] = m2l_fma(D[73], m, L[26]);
+      L[27] = m2l_fma(D[74], m, L[27]);
+      L[28] = m2l_fma(D[75], m, L[28]);
+      L[29] = m2l_fma(D[76], m, L[29]);
+      L[30] = m2l_fma(D[79], m, L[30]);
+      L[31] = m2l_fma(D[80], m, L[31]);
+      L[32] = m2l_fma(D[81], m, L[32]);
+      L[33] = m2l_fma(D[82], m, L[33]);
+      L[34] = m2l_fma(D[83], m, L[34]);
     }
     rp *= rho;
-    { const float m = -__ldg(Ms + 35) * rp;
-      L[1] = fmaf(D[56], m, L[1]);
-      L[2] = fmaf(D[57], m, L[2]);
-      L[3] = fmaf(D[58], m, L[3]);
+    { const T m = -__ldg(Ms + 10) * rp;
+      L[1] = m2l_fma(D[20], m, L[1]);
+      L[2] = m2l_fma(D[21], m, L[2]);
+      L[3] = m2l_fma(D[22], m, L[3]);
+      L[4] = m2l_fma(D[35], m, L[4]);
+      L[5] = m2l_fma(D[36], m, L[5]);
+      L[6] = m2l_fma(D[37], m, L[6]);
+      L[7] = m2l_fma(D[38], m, L[7]);
+      L[8] = m2l_fma(D[39], m, L[8]);
+      L[9] = m2l_fma(D[40], m, L[9]);
+      L[10] = m2l_fma(D[56], m, L[10]);
+      L[11] = m2l_fma(D[57], m, L[11]);
+      L[12] = m2l_fma(D[58], m, L[12]);
+      L[13] = m2l_fma(D[59], m, L[13]);
+      L[14] = m2l_fma(D[60], m, L[14]);
+      L[15] = m2l_fma(D[61], m, L[15]);
+      L[16] = m2l_fma(D[62], m, L[16]);
+      L[17] = m2l_fma(D[63], m, L[17]);
+      L[18] = m2l_fma(D[64], m, L[18]);
+      L[19] = m2l_fma(D[65], m, L[19]);
     }
-    { const float m = -__ldg(Ms + 36) * rp;
-      L[1] = fmaf(D[57], m, L[1]);
-      L[2] = fmaf(D[59], m, L[2]);
-      L[3] = fmaf(D[60], m, L[3]);
+    { const T m = -__ldg(Ms + 11) * rp;
+      L[1] = m2l_fma(D[21], m, L[1]);
+      L[2] = m2l_fma(D[23], m, L[2]);
+      L[3] = m2l_fma(D[24], m, L[3]);
+      L[4] = m2l_fma(D[36], m, L[4]);
+      L[5] = m2l_fma(D[38], m, L[5]);
+      L[6] = m2l_fma(D[39], m, L[6]);
+      L[7] = m2l_fma(D[41], m, L[7]);
+      L[8] = m2l_fma(D[42], m, L[8]);
+      L[9] = m2l_fma(D[43], m, L[9]);
+      L[10] = m2l_fma(D[57], m, L[10]);
+      L[11] = m2l_fma(D[59], m, L[11]);
+      L[12] = m2l_fma(D[60], m, L[12]);
+      L[13] = m2l_fma(D[62], m, L[13]);
+      L[14] = m2l_fma(D[63], m, L[14]);
+      L[15] = m2l_fma(D[64], m, L[15]);
+      L[16] = m2l_fma(D[66], m, L[16]);
+      L[17] = m2l_fma(D[67], m, L[17]);
+      L[18] = m2l_fma(D[68], m, L[18]);
+      L[19] = m2l_fma(D[69], m, L[19]);
     }
-    { const float m = -__ldg(Ms + 37) * rp;
-      L[1] = fmaf(D[58], m, L[1]);
-      L[2] = fmaf(D[60], m, L[2]);
-      L[3] = fmaf(D[61], m, L[3]);
+    { const T m = -__ldg(Ms + 12) * rp;
+      L[1] = m2l_fma(D[22], m, L[1]);
+      L[2] = m2l_fma(D[24], m, L[2]);
+      L[3] = m2l_fma(D[25], m, L[3]);
+      L[4] = m2l_fma(D[37], m, L[4]);
+      L[5] = m2l_fma(D[39], m, L[5]);
+      L[6] = m2l_fma(D[40], m, L[6]);
+      L[7] = m2l_fma(D[42], m, L[7]);
+      L[8] = m2l_fma(D[43], m, L[8]);
+      L[9] = m2l_fma(D[44], m, L[9]);
+      L[10] = m2l_fma(D[58], m, L[10]);
+      L[11] = m2l_fma(D[60], m, L[11]);
+      L[12] = m2l_fma(D[61], m, L[12]);
+      L[13] = m2l_fma(D[63], m, L[13]);
+      L[14] = m2l_fma(D[64], m, L[14]);
+      L[15] = m2l_fma(D[65], m, L[15]);
+      L[16] = m2l_fma(D[67], m, L[16]);
+      L[17] = m2l_fma(D[68], m, L[17]);
+      L[18] = m2l_fma(D[69], m, L[18]);
+      L[19] = m2l_fma(D[70], m, L[19]);
     }
-    { const float m = -__ldg(Ms + 38) * rp;
-      L[1] = fmaf(D[59], m, L[1]);
-      L[2] = fmaf(D[62], m, L[2]);
-      L[3] = fmaf(D[63], m, L[3]);
+    { const T m = -__ldg(Ms + 13) * rp;
+      L[1] = m2l_fma(D[23], m, L[1]);
+      L[2] = m2l_fma(D[26], m, L[2]);
+      L[3] = m2l_fma(D[27], m, L[3]);
+      L[4] = m2l_fma(D[38], m, L[4]);
+      L[5] = m2l_fma(D[41], m, L[5]);
+      L[6] = m2l_fma(D[42], m, L[6]);
+      L[7] = m2l_fma(D[45], m, L[7]);
+      L[8] = m2l_fma(D[46], m, L[8]);
+      L[9] = m2l_fma(D[47], m, L[9]);
+      L[10] = m2l_fma(D[59], m, L[10]);
+      L[11] = m2l_fma(D[62], m, L[11]);
+      L[12] = m2l_fma(D[63], m, L[12]);
+      L[13] = m2l_fma(D[66], m, L[13]);
+      L[14] = m2l_fma(D[67], m, L[14]);
+      L[15] = m2l_fma(D[68], m, L[15]);
+      L[16] = m2l_fma(D[71], m, L[16]);
+      L[17] = m2l_fma(D[72], m, L[17]);
+      L[18] = m2l_fma(D[73], m, L[18]);
+      L[19] = m2l_fma(D[74], m, L[19]);
     }
-    { const float m = -__ldg(Ms + 39) * rp;
-      L[1] = fmaf(D[60], m, L[1]);
-      L[2] = fmaf(D[63], m, L[2]);
-      L[3] = fmaf(D[64], m, L[3]);
+    { const T m = -__ldg(Ms + 14) * rp;
+      L[1] = m2l_fma(D[24], m, L[1]);
+      L[2] = m2l_fma(D[27], m, L[2]);
+      L[3] = m2l_fma(D[28], m, L[3]);
+      L[4] = m2l_fma(D[39], m, L[4]);
+      L[5] = m2l_fma(D[42], m, L[5]);
+      L[6] = m2l_fma(D[43], m, L[6]);
+      L[7] = m2l_fma(D[46], m, L[7]);
+      L[8] = m2l_fma(D[47], m, L[8]);
+      L[9] = m2l_fma(D[48], m, L[9]);
+      L[10] = m2l_fma(D[60], m, L[10]);
+      L[11] = m2l_fma(D[63], m, L[11]);
+      L[12] = m2l_fma(D[64], m, L[12]);
+      L[13] = m2l_fma(D[67], m, L[13]);
+      L[14] = m2l_fma(D[68], m, L[14]);
+      L[15] = m2l_fma(D[69], m, L[15]);
+      L[16] = m2l_fma(D[72], m, L[16]);
+      L[17] = m2l_fma(D[73], m, L[17]);
+      L[18] = m2l_fma(D[74], m, L[18]);
+      L[19] = m2l_fma(D[75], m, L[19]);
     }
-    { const float m = -__ldg(Ms + 40) * rp;
-      L[1] = fmaf(D[61], m, L[1]);
-      L[2] = fmaf(D[64], m, L[2]);
-      L[3] = fmaf(D[65], m, L[3]);
+    { const T m = -__ldg(Ms + 15) * rp;
+      L[1] = m2l_fma(D[25], m, L[1]);
+      L[2] = m2l_fma(D[28], m, L[2]);
+      L[3] = m2l_fma(D[29], m, L[3]);
+      L[4] = m2l_fma(D[40], m, L[4]);
+      L[5] = m2l_fma(D[43], m, L[5]);
+      L[6] = m2l_fma(D[44], m, L[6]);
+      L[7] = m2l_fma(D[47], m, L[7]);
+      L[8] = m2l_fma(D[48], m, L[8]);
+      L[9] = m2l_fma(D[49], m, L[9]);
+      L[10] = m2l_fma(D[61], m, L[10]);
+      L[11] = m2l_fma(D[64], m, L[11]);
+      L[12] = m2l_fma(D[65], m, L[12]);
+      L[13] = m2l_fma(D[68], m, L[13]);
+      L[14] = m2l_fma(D[69], m, L[14]);
+      L[15] = m2l_fma(D[70], m, L[15]);
+      L[16] = m2l_fma(D[73], m, L[16]);
+      L[17] = m2l_fma(D[74], m, L[17]);
+      L[18] = m2l_fma(D[75], m, L[18]);
+      L[19] = m2l_fma(D[76], m, L[19]);
     }
-    { const float m = -__ldg(Ms + 41) * rp;
-      L[1] = fmaf(D[62], m, L[1]);
-      L[2] = fmaf(D[66], m, L[2]);
-      L[3] = fmaf(D[67], m, L[3]);
+    { const T m = -__ldg(Ms + 16) * rp;
+      L[1] = m2l_fma(D[26], m, L[1]);
+      L[2] = m2l_fma(D[30], m, L[2]);
+      L[3] = m2l_fma(D[31], m, L[3]);
+      L[4] = m2l_fma(D[41], m, L[4]);
+      L[5] = m2l_fma(D[45], m, L[5]);
+      L[6] = m2l_fma(D[46], m, L[6]);
+      L[7] = m2l_fma(D[50], m, L[7]);
+      L[8] = m2l_fma(D[51], m, L[8]);
+      L[9] = m2l_fma(D[52], m, L[9]);
+      L[10] = m2l_fma(D[62], m, L[10]);
+      L[11] = m2l_fma(D[66], m, L[11]);
+      L[12] = m2l_fma(D[67], m, L[12]);
+      L[13] = m2l_fma(D[71], m, L[13]);
+      L[14] = m2l_fma(D[72], m, L[14]);
+      L[15] = m2l_fma(D[73], m, L[15]);
+      L[16] = m2l_fma(D[77], m, L[16]);
+      L[17] = m2l_fma(D[78], m, L[17]);
+      L[18] = m2l_fma(D[79], m, L[18]);
+      L[19] = m2l_fma(D[80], m, L[19]);
     }
-    { const float m = -__ldg(Ms + 42) * rp;
-      L[1] = fmaf(D[63], m, L[1]);
-      L[2] = fmaf(D[67], m, L[2]);
-      L[3] = fmaf(D[68], m, L[3]);
+    { const T m = -__ldg(Ms + 17) * rp;
+      L[1] = m2l_fma(D[27], m, L[1]);
+      L[2] = m2l_fma(D[31], m, L[2]);
+      L[3] = m2l_fma(D[32], m, L[3]);
+      L[4] = m2l_fma(D[42], m, L[4]);
+      L[5] = m2l_fma(D[46], m, L[5]);
+      L[6] = m2l_fma(D[47], m, L[6]);
+      L[7] = m2l_fma(D[51], m, L[7]);
+      L[8] = m2l_fma(D[52], m, L[8]);
+      L[9] = m2l_fma(D[53], m, L[9]);
+      L[10] = m2l_fma(D[63], m, L[10]);
+      L[11] = m2l_fma(D[67], m, L[11]);
+      L[12] = m2l_fma(D[68], m, L[12]);
+      L[13] = m2l_fma(D[72], m, L[13]);
+      L[14] = m2l_fma(D[73], m, L[14]);
+      L[15] = m2l_fma(D[74], m, L[15]);
+      L[16] = m2l_fma(D[78], m, L[16]);
+      L[17] = m2l_fma(D[79], m, L[17]);
+      L[18] = m2l_fma(D[80], m, L[18]);
+      L[19] = m2l_fma(D[81], m, L[19]);
     }
-    { const float m = -__ldg(Ms + 43) * rp;
-      L[1] = fmaf(D[64], m, L[1]);
-      L[2] = fmaf(D[68], m, L[2]);
-      L[3] = fmaf(D[69], m, L[3]);
+    { const T m = -__ldg(Ms + 18) * rp;
+      L[1] = m2l_fma(D[28], m, L[1]);
+      L[2] = m2l_fma(D[32], m, L[2]);
+      L[3] = m2l_fma(D[33], m, L[3]);
+      L[4] = m2l_fma(D[43], m, L[4]);
+      L[5] = m2l_fma(D[47], m, L[5]);
+      L[6] = m2l_fma(D[48], m, L[6]);
+      L[7] = m2l_fma(D[52], m, L[7]);
+      L[8] = m2l_fma(D[53], m, L[8]);
+      L[9] = m2l_fma(D[54], m, L[9]);
+      L[10] = m2l_fma(D[64], m, L[10]);
+      L[11] = m2l_fma(D[68], m, L[11]);
+      L[12] = m2l_fma(D[69], m, L[12]);
+      L[13] = m2l_fma(D[73], m, L[13]);
+      L[14] = m2l_fma(D[74], m, L[14]);
+      L[15] = m2l_fma(D[75], m, L[15]);
+      L[16] = m2l_fma(D[79], m, L[16]);
+      L[17] = m2l_fma(D[80], m, L[17]);
+      L[18] = m2l_fma(D[81], m, L[18]);
+      L[19] = m2l_fma(D[82], m, L[19]);
     }
-    { const float m = -__ldg(Ms + 44) * rp;
-      L[1] = fmaf(D[65], m, L[1]);
-      L[2] = fmaf(D[69], m, L[2]);
-      L[3] = fmaf(D[70], m, L[3]);
+    { const T m = -__ldg(Ms + 19) * rp;
+      L[1] = m2l_fma(D[29], m, L[1]);
+      L[2] = m2l_fma(D[33], m, L[2]);
+      L[3] = m2l_fma(D[34], m, L[3]);
+      L[4] = m2l_fma(D[44], m, L[4]);
+      L[5] = m2l_fma(D[48], m, L[5]);
+      L[6] = m2l_fma(D[49], m, L[6]);
+      L[7] = m2l_fma(D[53], m, L[7]);
+      L[8] = m2l_fma(D[54], m, L[8]);
+      L[9] = m2l_fma(D[55], m, L[9]);
+      L[10] = m2l_fma(D[65], m, L[10]);
+      L[11] = m2l_fma(D[69], m, L[11]);
+      L[12] = m2l_fma(D[70], m, L[12]);
+      L[13] = m2l_fma(D[74], m, L[13]);
+      L[14] = m2l_fma(D[75], m, L[14]);
+      L[15] = m2l_fma(D[76], m, L[15]);
+      L[16] = m2l_fma(D[80], m, L[16]);
+      L[17] = m2l_fma(D[81], m, L[17]);
+      L[18] = m2l_fma(D[82], m, L[18]);
+      L[19] = m2l_fma(D[83], m, L[19]);
     }
-    { const float m = -__ldg(Ms + 45) * rp;
-      L[1] = fmaf(D[66], m, L[1]);
-      L[2] = fmaf(D[71], m, L[2]);
-      L[3] = fmaf(D[72], m, L[3]);
+    rp *= rho;
+    { const T m = __ldg(Ms + 20) * rp;
+      L[1] = m2l_fma(D[35], m, L[1]);
+      L[2] = m2l_fma(D[36], m, L[2]);
+      L[3] = m2l_fma(D[37], m, L[3]);
+      L[4] = m2l_fma(D[56], m, L[4]);
+      L[5] = m2l_fma(D[57], m, L[5]);
+      L[6] = m2l_fma(D[58], m, L[6]);
+      L[7] = m2l_fma(D[59], m, L[7]);
+      L[8] = m2l_fma(D[60], m, L[8]);
+      L[9] = m2l_fma(D[61], m, L[9]);
     }
-    { const float m = -__ldg(Ms + 46) * rp;
-      L[1] = fmaf(D[67], m, L[1]);
-      L[2] = fmaf(D[72], m, L[2]);
-      L[3] = fmaf(D[73], m, L[3]);
+    { const T m = __ldg(Ms + 21) * rp;
+      L[1] = m2l_fma(D[36], m, L[1]);
+      L[2] = m2l_fma(D[38], m, L[2]);
+      L[3] = m2l_fma(D[39], m, L[3]);
+      L[4] = m2l_fma(D[57], m, L[4]);
+      L[5] = m2l_fma(D[59], m, L[5]);
+      L[6] = m2l_fma(D[60], m, L[6]);
+      L[7] = m2l_fma(D[62], m, L[7]);
+      L[8] = m2l_fma(D[63], m, L[8]);
+      L[9] = m2l_fma(D[64], m, L[9]);
     }
-    { const float m = -__ldg(Ms + 47) * rp;
-      L[1] = fmaf(D[68], m, L[1]);
-      L[2] = fmaf(D[73], m, L[2]);
-      L[3] = fmaf(D[74], m, L[3]);
+    { const T m = __ldg(Ms + 22) * rp;
+      L[1] = m2l_fma(D[37], m, L[1]);
+      L[2] = m2l_fma(D[39], m, L[2]);
+      L[3] = m2l_fma(D[40], m, L[3]);
+      L[4] = m2l_fma(D[58], m, L[4]);
+      L[5] = m2l_fma(D[60], m, L[5]);
+      L[6] = m2l_fma(D[61], m, L[6]);
+      L[7] = m2l_fma(D[63], m, L[7]);
+      L[8] = m2l_fma(D[64], m, L[8]);
+      L[9] = m2l_fma(D[65], m, L[9]);
     }
-    { const float m = -__ldg(Ms + 48) * rp;
-      L[1] = fmaf(D[69], m, L[1]);
-      L[2] = fmaf(D[74], m, L[2]);
-      L[3] = fmaf(D[75], m, L[3]);
+    { const T m = __ldg(Ms + 23) * rp;
+      L[1] = m2l_fma(D[38], m, L[1]);
+      L[2] = m2l_fma(D[41], m, L[2]);
+      L[3] = m2l_fma(D[42], m, L[3]);
+      L[4] = m2l_fma(D[59], m, L[4]);
+      L[5] = m2l_fma(D[62], m, L[5]);
+      L[6] = m2l_fma(D[63], m, L[6]);
+      L[7] = m2l_fma(D[66], m, L[7]);
+      L[8] = m2l_fma(D[67], m, L[8]);
+      L[9] = m2l_fma(D[68], m, L[9]);
     }
-    { const float m = -__ldg(Ms + 49) * rp;
-      L[1] = fmaf(D[70], m, L[1]);
-      L[2] = fmaf(D[75], m, L[2]);
-      L[3] = fmaf(D[76], m, L[3]);
+    { const T m = __ldg(Ms + 24) * rp;
+      L[1] = m2l_fma(D[39], m, L[1]);
+      L[2] = m2l_fma(D[42], m, L[2]);
+      L[3] = m2l_fma(D[43], m, L[3]);
+      L[4] = m2l_fma(D[60], m, L[4]);
+      L[5] = m2l_fma(D[63], m, L[5]);
+      L[6] = m2l_fma(D[64], m, L[6]);
+      L[7] = m2l_fma(D[67], m, L[7]);
+      L[8] = m2l_fma(D[68], m, L[8]);
+      L[9] = m2l_fma(D[69], m, L[9]);
     }
-    { const float m = -__ldg(Ms + 50) * rp;
-      L[1] = fmaf(D[71], m, L[1]);
-      L[2] = fmaf(D[77], m, L[2]);
-      L[3] = fmaf(D[78], m, L[3]);
+    { const T m = __ldg(Ms + 25) * rp;
+      L[1] = m2l_fma(D[40], m, L[1]);
+      L[2] = m2l_fma(D[43], m, L[2]);
+      L[3] = m2l_fma(D[44], m, L[3]);
+      L[4] = m2l_fma(D[61], m, L[4]);
+      L[5] = m2l_fma(D[64], m, L[5]);
+      L[6] = m2l_fma(D[65], m, L[6]);
+      L[7] = m2l_fma(D[68], m, L[7]);
+      L[8] = m2l_fma(D[69], m, L[8]);
+      L[9] = m2l_fma(D[70], m, L[9]);
     }
-    { const float m = -__ldg(Ms + 51) * rp;
-      L[1] = fmaf(D[72], m, L[1]);
-      L[2] = fmaf(D[78], m, L[2]);
-      L[3] = fmaf(D[79], m, L[3]);
+    { const T m = __ldg(Ms + 26) * rp;
+      L[1] = m2l_fma(D[41], m, L[1]);
+      L[2] = m2l_fma(D[45], m, L[2]);
+      L[3] = m2l_fma(D[46], m, L[3]);
+      L[4] = m2l_fma(D[62], m, L[4]);
+      L[5] = m2l_fma(D[66], m, L[5]);
+      L[6] = m2l_fma(D[67], m, L[6]);
+      L[7] = m2l_fma(D[71], m, L[7]);
+      L[8] = m2l_fma(D[72], m, L[8]);
+      L[9] = m2l_fma(D[73], m, L[9]);
     }
-    { const float m = -__ldg(Ms + 52) * rp;
-      L[1] = fmaf(D[73], m, L[1]);
-      L[2] = fmaf(D[79], m, L[2]);
-      L[3] = fmaf(D[80], m, L[3]);
+    { const T m = __ldg(Ms + 27) * rp;
+      L[1] = m2l_fma(D[42], m, L[1]);
+      L[2] = m2l_fma(D[46], m, L[2]);
+      L[3] = m2l_fma(D[47], m, L[3]);
+      L[4] = m2l_fma(D[63], m, L[4]);
+      L[5] = m2l_fma(D[67], m, L[5]);
+      L[6] = m2l_fma(D[68], m, L[6]);
+      L[7] = m2l_fma(D[72], m, L[7]);
+      L[8] = m2l_fma(D[73], m, L[8]);
+      L[9] = m2l_fma(D[74], m, L[9]);
     }
-    { const float m = -__ldg(Ms + 53) * rp;
-      L[1] = fmaf(D[74], m, L[1]);
-      L[2] = fmaf(D[80], m, L[2]);
-      L[3] = fmaf(D[81], m, L[3]);
+    { const T m = __ldg(Ms + 28) * rp;
+      L[1] = m2l_fma(D[43], m, L[1]);
+      L[2] = m2l_fma(D[47], m, L[2]);
+      L[3] = m2l_fma(D[48], m, L[3]);
+      L[4] = m2l_fma(D[64], m, L[4]);
+      L[5] = m2l_fma(D[68], m, L[5]);
+      L[6] = m2l_fma(D[69], m, L[6]);
+      L[7] = m2l_fma(D[73], m, L[7]);
+      L[8] = m2l_fma(D[74], m, L[8]);
+      L[9] = m2l_fma(D[75], m, L[9]);
     }
-    { const float m = -__ldg(Ms + 54) * rp;
-      L[1] = fmaf(D[75], m, L[1]);
-      L[2] = fmaf(D[81], m, L[2]);
-      L[3] = fmaf(D[82], m, L[3]);
+    { const T m = __ldg(Ms + 29) * rp;
+      L[1] = m2l_fma(D[44], m, L[1]);
+      L[2] = m2l_fma(D[48], m, L[2]);
+      L[3] = m2l_fma(D[49], m, L[3]);
+      L[4] = m2l_fma(D[65], m, L[4]);
+      L[5] = m2l_fma(D[69], m, L[5]);
+      L[6] = m2l_fma(D[70], m, L[6]);
+      L[7] = m2l_fma(D[74], m, L[7]);
+      L[8] = m2l_fma(D[75], m, L[8]);
+      L[9] = m2l_fma(D[76], m, L[9]);
     }
-    { const float m = -__ldg(Ms + 55) * rp;
-      L[1] = fmaf(D[76], m, L[1]);
-      L[2] = fmaf(D[82], m, L[2]);
-      L[3] = fmaf(D[83], m, L[3]);
+    { const T m = __ldg(Ms + 30) * rp;
+      L[1] = m2l_fma(D[45], m, L[1]);
+      L[2] = m2l_fma(D[50], m, L[2]);
+      L[3] = m2l_fma(D[51], m, L[3]);
+      L[4] = m2l_fma(D[66], m, L[4]);
+      L[5] = m2l_fma(D[71], m, L[5]);
+      L[6] = m2l_fma(D[72], m, L[6]);
+      L[7] = m2l_fma(D[77], m, L[7]);
+      L[8] = m2l_fma(D[78], m, L[8]);
+      L[9] = m2l_fma(D[79], m, L[9]);
+    }
+    { const T m = __ldg(Ms + 31) * rp;
+      L[1] = m2l_fma(D[46], m, L[1]);
+      L[2] = m2l_fma(D[51], m, L[2]);
+      L[3] = m2l_fma(D[52], m, L[3]);
+      L[4] = m2l_fma(D[67], m, L[4]);
+      L[5] = m2l_fma(D[72], m, L[5]);
+      L[6] = m2l_fma(D[73], m, L[6]);
+      L[7] = m2l_fma(D[78], m, L[7]);
+      L[8] = m2l_fma(D[79], m, L[8]);
+      L[9] = m2l_fma(D[80], m, L[9]);
+    }
+    { const T m = __ldg(Ms + 32) * rp;
+      L[1] = m2l_fma(D[47], m, L[1]);
+      L[2] = m2l_fma(D[52], m, L[2]);
+      L[3] = m2l_fma(D[53], m, L[3]);
+      L[4] = m2l_fma(D[68], m, L[4]);
+      L[5] = m2l_fma(D[73], m, L[5]);
+      L[6] = m2l_fma(D[74], m, L[6]);
+      L[7] = m2l_fma(D[79], m, L[7]);
+      L[8] = m2l_fma(D[80], m, L[8]);
+      L[9] = m2l_fma(D[81], m, L[9]);
+    }
+    { const T m = __ldg(Ms + 33) * rp;
+      L[1] = m2l_fma(D[48], m, L[1]);
+      L[2] = m2l_fma(D[53], m, L[2]);
+      L[3] = m2l_fma(D[54], m, L[3]);
+      L[4] = m2l_fma(D[69], m, L[4]);
+      L[5] = m2l_fma(D[74], m, L[5]);
+      L[6] = m2l_fma(D[75], m, L[6]);
+      L[7] = m2l_fma(D[80], m, L[7]);
+      L[8] = m2l_fma(D[81], m, L[8]);
+      L[9] = m2l_fma(D[82], m, L[9]);
+    }
+    { const T m = __ldg(Ms + 34) * rp;
+      L[1] = m2l_fma(D[49], m, L[1]);
+      L[2] = m2l_fma(D[54], m, L[2]);
+      L[3] = m2l_fma(D[55], m, L[3]);
+      L[4] = m2l_fma(D[70], m, L[4]);
+      L[5] = m2l_fma(D[75], m, L[5]);
+      L[6] = m2l_fma(D[76], m, L[6]);
+      L[7] = m2l_fma(D[81], m, L[7]);
+      L[8] = m2l_fma(D[82], m, L[8]);
+      L[9] = m2l_fma(D[83], m, L[9]);
+    }
+    rp *= rho;
+    { const T m = -__ldg(Ms + 35) * rp;
+      L[1] = m2l_fma(D[56], m, L[1]);
+      L[2] = m2l_fma(D[57], m, L[2]);
+      L[3] = m2l_fma(D[58], m, L[3]);
+    }
+    { const T m = -__ldg(Ms + 36) * rp;
+      L[1] = m2l_fma(D[57], m, L[1]);
+      L[2] = m2l_fma(D[59], m, L[2]);
+      L[3] = m2l_fma(D[60], m, L[3]);
+    }
+    { const T m = -__ldg(Ms + 37) * rp;
+      L[1] = m2l_fma(D[58], m, L[1]);
+      L[2] = m2l_fma(D[60], m, L[2]);
+      L[3] = m2l_fma(D[61], m, L[3]);
+    }
+    { const T m = -__ldg(Ms + 38) * rp;
+      L[1] = m2l_fma(D[59], m, L[1]);
+      L[2] = m2l_fma(D[62], m, L[2]);
+      L[3] = m2l_fma(D[63], m, L[3]);
+    }
+    { const T m = -__ldg(Ms + 39) * rp;
+      L[1] = m2l_fma(D[60], m, L[1]);
+      L[2] = m2l_fma(D[63], m, L[2]);
+      L[3] = m2l_fma(D[64], m, L[3]);
+    }
+    { const T m = -__ldg(Ms + 40) * rp;
+      L[1] = m2l_fma(D[61], m, L[1]);
+      L[2] = m2l_fma(D[64], m, L[2]);
+      L[3] = m2l_fma(D[65], m, L[3]);
+    }
+    { const T m = -__ldg(Ms + 41) * rp;
+      L[1] = m2l_fma(D[62], m, L[1]);
+      L[2] = m2l_fma(D[66], m, L[2]);
+      L[3] = m2l_fma(D[67], m, L[3]);
+    }
+    { const T m = -__ldg(Ms + 42) * rp;
+      L[1] = m2l_fma(D[63], m, L[1]);
+      L[2] = m2l_fma(D[67], m, L[2]);
+      L[3] = m2l_fma(D[68], m, L[3]);
+    }
+    { const T m = -__ldg(Ms + 43) * rp;
+      L[1] = m2l_fma(D[64], m, L[1]);
+      L[2] = m2l_fma(D[68], m, L[2]);
+      L[3] = m2l_fma(D[69], m, L[3]);
+    }
+    { const T m = -__ldg(Ms + 44) * rp;
+      L[1] = m2l_fma(D[65], m, L[1]);
+      L[2] = m2l_fma(D[69], m, L[2]);
+      L[3] = m2l_fma(D[70], m, L[3]);
+    }
+    { const T m = -__ldg(Ms + 45) * rp;
+      L[1] = m2l_fma(D[66], m, L[1]);
+      L[2] = m2l_fma(D[71], m, L[2]);
+      L[3] = m2l_fma(D[72], m, L[3]);
+    }
+    { const T m = -__ldg(Ms + 46) * rp;
+      L[1] = m2l_fma(D[67], m, L[1]);
+      L[2] = m2l_fma(D[72], m, L[2]);
+      L[3] = m2l_fma(D[73], m, L[3]);
+    }
+    { const T m = -__ldg(Ms + 47) * rp;
+      L[1] = m2l_fma(D[68], m, L[1]);
+      L[2] = m2l_fma(D[73], m, L[2]);
+      L[3] = m2l_fma(D[74], m, L[3]);
+    }
+    { const T m = -__ldg(Ms + 48) * rp;
+      L[1] = m2l_fma(D[69], m, L[1]);
+      L[2] = m2l_fma(D[74], m, L[2]);
+      L[3] = m2l_fma(D[75], m, L[3]);
+    }
+    { const T m = -__ldg(Ms + 49) * rp;
+      L[1] = m2l_fma(D[70], m, L[1]);
+      L[2] = m2l_fma(D[75], m, L[2]);
+      L[3] = m2l_fma(D[76], m, L[3]);
+    }
+    { const T m = -__ldg(Ms + 50) * rp;
+      L[1] = m2l_fma(D[71], m, L[1]);
+      L[2] = m2l_fma(D[77], m, L[2]);
+      L[3] = m2l_fma(D[78], m, L[3]);
+    }
+    { const T m = -__ldg(Ms + 51) * rp;
+      L[1] = m2l_fma(D[72], m, L[1]);
+      L[2] = m2l_fma(D[78], m, L[2]);
+      L[3] = m2l_fma(D[79], m, L[3]);
+    }
+    { const T m = -__ldg(Ms + 52) * rp;
+      L[1] = m2l_fma(D[73], m, L[1]);
+      L[2] = m2l_fma(D[79], m, L[2]);
+      L[3] = m2l_fma(D[80], m, L[3]);
+    }
+    { const T m = -__ldg(Ms + 53) * rp;
+      L[1] = m2l_fma(D[74], m, L[1]);
+      L[2] = m2l_fma(D[80], m, L[2]);
+      L[3] = m2l_fma(D[81], m, L[3]);
+    }
+    { const T m = -__ldg(Ms + 54) * rp;
+      L[1] = m2l_fma(D[75], m, L[1]);
+      L[2] = m2l_fma(D[81], m, L[2]);
+      L[3] = m2l_fma(D[82], m, L[3]);
+    }
+    { const T m = -__ldg(Ms + 55) * rp;
+      L[1] = m2l_fma(D[76], m, L[1]);
+      L[2] = m2l_fma(D[82], m, L[2]);
+      L[3] = m2l_fma(D[83], m, L[3]);
     }
 }
 
-__device__ __forceinline__ void m2l_side_b_forces_6(const float (&D)[84], const float *__restrict__ Ms, float (&L)[84])
+template <class T> __device__ __forceinline__ void m2l_side_b_forces_6(const T (&D)[84], const T *__restrict__ Ms, T (&L)[84])
 {
-    L[0] = 0.0f;
-    { const float m = __ldg(Ms + 0);
+    L[0] = T(0);
+    { const T m = __ldg(Ms + 0);
       L[1] = -D[1] * m;
       L[2] = -D[2] * m;
       L[3] = -D[3] * m;
@@ -7815,1077 +7820,1075 @@ __device__ __forceinline__ void m2l_side_b_forces_6(const float (&D)[84], const 
       L[82] = D[82] * m;
       L[83] = D[83] * m;
     }
-    { const float m = __ldg(Ms + 1);
-      L[1] = fmaf(-D[4], m, L[1]);
-      L[2] = fmaf(-D[5], m, L[2]);
-      L[3] = fmaf(-D[6], m, L[3]);
-      L[4] = fmaf(D[10], m, L[4]);
-      L[5] = fmaf(D[11], m, L[5]);
-      L[6] = fmaf(D[12], m, L[6]);
-      L[7] = fmaf(D[13], m, L[7]);
-      L[8] = fmaf(D[14], m, L[8]);
-      L[9] = fmaf(D[15], m, L[9]);
-      L[10] = fmaf(-D[20], m, L[10]);
-      L[11] = fmaf(-D[21], m, L[11]);
-      L[12] = fmaf(-D[22], m, L[12]);
-      L[13] = fmaf(-D[23], m, L[13]);
-      L[14] = fmaf(-D[24], m, L[14]);
-      L[15] = fmaf(-D[25], m, L[15]);
-      L[16] = fmaf(-D[26], m, L[16]);
-      L[17] = fmaf(-D[27], m, L[17]);
-      L[18] = fmaf(-D[28], m, L[18]);
-      L[19] = fmaf(-D[29], m, L[19]);
-      L[20] = fmaf(D[35], m, L[20]);
-      L[21] = fmaf(D[36], m, L[21]);
-      L[22] = fmaf(D[37], m, L[22]);
-      L[23] = fmaf(D[38], m, L[23]);
-      L[24] = fmaf(D[39], m, L[24]);
-      L[25] = fmaf(D[40], m, L[25]);
-      L[26] = fmaf(D[41], m, L[26]);
-      L[27] = fmaf(D[42], m, L[27]);
-      L[28] = fmaf(D[43], m, L[28]);
-      L[29] = fmaf(D[44], m, L[29]);
-      L[30] = fmaf(D[45], m, L[30]);
-      L[31] = fmaf(D[46], m, L[31]);
-      L[32] = fmaf(D[47], m, L[32]);
-      L[33] = fmaf(D[48], m, L[33]);
-      L[34] = fmaf(D[49], m, L[34]);
-      L[35] = fmaf(-D[56], m, L[35]);
-      L[36] = fmaf(-D[57], m, L[36]);
-      L[37] = fmaf(-D[58], m, L[37]);
-      L[38] = fmaf(-D[59], m, L[38]);
-      L[39] = fmaf(-D[60], m, L[39]);
-      L[40] = fmaf(-D[61], m, L[40]);
-      L[41] = fmaf(-D[62], m, L[41]);
-      L[42] = fmaf(-D[63], m, L[42]);
-      L[43] = fmaf(-D[64], m, L[43]);
-      L[44] = fmaf(-D[65], m, L[44]);
-      L[45] = fmaf(-D[66], m, L[45]);
-      L[46] = fmaf(-D[67], m, L[46]);
-      L[47] = fmaf(-D[68], m, L[47]);
-      L[48] = fmaf(-D[69], m, L[48]);
-      L[49] = fmaf(-D[70], m, L[49]);
-      L[50] = fmaf(-D[71], m, L[50]);
-      L[51] = fmaf(-D[72], m, L[51]);
-      L[52] = fmaf(-D[73], m, L[52]);
-      L[53] = fmaf(-D[74], m, L[53]);
-      L[54] = fmaf(-D[75], m, L[54]);
-      L[55] = fmaf(-D[76], m, L[55]);
+    { const T m = __ldg(Ms + 1);
+      L[1] = m2l_fma(-D[4], m, L[1]);
+      L[2] = m2l_fma(-D[5], m, L[2]);
+      L[3] = m2l_fma(-D[6], m, L[3]);
+      L[4] = m2l_fma(D[10], m, L[4]);
+      L[5] = m2l_fma(D[11], m, L[5]);
+      L[6] = m2l_fma(D[12], m, L[6]);
+      L[7] = m2l_fma(D[13], m, L[7]);
+      L[8] = m2l_fma(D[14], m, L[8]);
+      L[9] = m2l_fma(D[15], m, L[9]);
+      L[10] = m2l_fma(-D[20], m, L[10]);
+      L[11] = m2l_fma(-D[21], m, L[11]);
+      L[12] = m2l_fma(-D[22], m, L[12]);
+      L[13] = m2l_fma(-D[23], m, L[13]);
+      L[14] = m2l_fma(-D[24], m, L[14]);
+      L[15] = m2l_fma(-D[25], m, L[15]);
+      L[16] = m2l_fma(-D[26], m, L[16]);
+      L[17] = m2l_fma(-D[27], m, L[17]);
+      L[18] = m2l_fma(-D[28], m, L[18]);
+      L[19] = m2l_fma(-D[29], m, L[19]);
+      L[20] = m2l_fma(D[35], m, L[20]);
+      L[21] = m2l_fma(D[36], m, L[21]);
+      L[22] = m2l_fma(D[37], m, L[22]);
+      L[23] = m2l_fma(D[38], m, L[23]);
+      L[24] = m2l_fma(D[39], m, L[24]);
+      L[25] = m2l_fma(D[40], m, L[25]);
+      L[26] = m2l_fma(D[41], m, L[26]);
+      L[27] = m2l_fma(D[42], m, L[27]);
+      L[28] = m2l_fma(D[43], m, L[28]);
+      L[29] = m2l_fma(D[44], m, L[29]);
+      L[30] = m2l_fma(D[45], m, L[30]);
+      L[31] = m2l_fma(D[46], m, L[31]);
+      L[32] = m2l_fma(D[47], m, L[32]);
+      L[33] = m2l_fma(D[48], m, L[33]);
+      L[34] = m2l_fma(D[49], m, L[34]);
+      L[35] = m2l_fma(-D[56], m, L[35]);
+      L[36] = m2l_fma(-D[57], m, L[36]);
+      L[37] = m2l_fma(-D[58], m, L[37]);
+      L[38] = m2l_fma(-D[59], m, L[38]);
+      L[39] = m2l_fma(-D[60], m, L[39]);
+      L[40] = m2l_fma(-D[61], m, L[40]);
+      L[41] = m2l_fma(-D[62], m, L[41]);
+      L[42] = m2l_fma(-D[63], m, L[42]);
+      L[43] = m2l_fma(-D[64], m, L[43]);
+      L[44] = m2l_fma(-D[65], m, L[44]);
+      L[45] = m2l_fma(-D[66], m, L[45]);
+      L[46] = m2l_fma(-D[67], m, L[46]);
+      L[47] = m2l_fma(-D[68], m, L[47]);
+      L[48] = m2l_fma(-D[69], m, L[48]);
+      L[49] = m2l_fma(-D[70], m, L[49]);
+      L[50] = m2l_fma(-D[71], m, L[50]);
+      L[51] = m2l_fma(-D[72], m, L[51]);
+      L[52] = m2l_fma(-D[73], m, L[52]);
+      L[53] = m2l_fma(-D[74], m, L[53]);
+      L[54] = m2l_fma(-D[75], m, L[54]);
+      L[55] = m2l_fma(-D[76], m, L[55]);
     }
-    { const float m = __ldg(Ms + 2);
-      L[1] = fmaf(-D[5], m, L[1]);
-      L[2] = fmaf(-D[7], m, L[2]);
-      L[3] = fmaf(-D[8], m, L[3]);
-      L[4] = fmaf(D[11], m, L[4]);
-      L[5] = fmaf(D[13], m, L[5]);
-      L[6] = fmaf(D[14], m, L[6]);
-      L[7] = fmaf(D[16], m, L[7]);
-      L[8] = fmaf(D[17], m, L[8]);
-      L[9] = fmaf(D[18], m, L[9]);
-      L[10] = fmaf(-D[21], m, L[10]);
-      L[11] = fmaf(-D[23], m, L[11]);
-      L[12] = fmaf(-D[24], m, L[12]);
-      L[13] = fmaf(-D[26], m, L[13]);
-      L[14] = fmaf(-D[27], m, L[14]);
-      L[15] = fmaf(-D[28], m, L[15]);
-      L[16] = fmaf(-D[30], m, L[16]);
-      L[17] = fmaf(-D[31], m, L[17]);
-      L[18] = fmaf(-D[32], m, L[18]);
-      L[19] = fmaf(-D[33], m, L[19]);
-      L[20] = fmaf(D[36], m, L[20]);
-      L[21] = fmaf(D[38], m, L[21]);
-      L[22] = fmaf(D[39], m, L[22]);
-      L[23] = fmaf(D[41], m, L[23]);
-      L[24] = fmaf(D[42], m, L[24]);
-      L[25] = fmaf(D[43], m, L[25]);
-      L[26] = fmaf(D[45], m, L[26]);
-      L[27] = fmaf(D[46], m, L[27]);
-      L[28] = fmaf(D[47], m, L[28]);
-      L[29] = fmaf(D[48], m, L[29]);
-      L[30] = fmaf(D[50], m, L[30]);
-      L[31] = fmaf(D[51], m, L[31]);
-      L[32] = fmaf(D[52], m, L[32]);
-      L[33] = fmaf(D[53], m, L[33]);
-      L[34] = fmaf(D[54], m, L[34]);
-      L[35] = fmaf(-D[57], m, L[35]);
-      L[36] = fmaf(-D[59], m, L[36]);
-      L[37] = fmaf(-D[60], m, L[37]);
-      L[38] = fmaf(-D[62], m, L[38]);
-      L[39] = fmaf(-D[63], m, L[39]);
-      L[40] = fmaf(-D[64], m, L[40]);
-      L[41] = fmaf(-D[66], m, L[41]);
-      L[42] = fmaf(-D[67], m, L[42]);
-      L[43] = fmaf(-D[68], m, L[43]);
-      L[44] = fmaf(-D[69], m, L[44]);
-      L[45] = fmaf(-D[71], m, L[45]);
-      L[46] = fmaf(-D[72], m, L[46]);
-      L[47] = fmaf(-D[73], m, L[47]);
-      L[48] = fmaf(-D[74], m, L[48]);
-      L[49] = fmaf(-D[75], m, L[49]);
-      L[50] = fmaf(-D[77], m, L[50]);
-      L[51] = fmaf(-D[78], m, L[51]);
-      L[52] = fmaf(-D[79], m, L[52]);
-      L[53] = fmaf(-D[80], m, L[53]);
-      L[54] = fmaf(-D[81], m, L[54]);
-      L[55] = fmaf(-D[82], m, L[55]);
+    { const T m = __ldg(Ms + 2);
+      L[1] = m2l_fma(-D[5], m, L[1]);
+      L[2] = m2l_fma(-D[7], m, L[2]);
+      L[3] = m2l_fma(-D[8], m, L[3]);
+      L[4] = m2l_fma(D[11], m, L[4]);
+      L[5] = m2l_fma(D[13], m, L[5]);
+      L[6] = m2l_fma(D[14], m, L[6]);
+      L[7] = m2l_fma(D[16], m, L[7]);
+      L[8] = m2l_fma(D[17], m, L[8]);
+      L[9] = m2l_fma(D[18], m, L[9]);
+      L[10] = m2l_fma(-D[21], m, L[10]);
+      L[11] = m2l_fma(-D[23], m, L[11]);
+      L[12] = m2l_fma(-D[24], m, L[12]);
+      L[13] = m2l_fma(-D[26], m, L[13]);
+      L[14] = m2l_fma(-D[27], m, L[14]);
+      L[15] = m2l_fma(-D[28], m, L[15]);
+      L[16] = m2l_fma(-D[30], m, L[16]);
+      L[17] = m2l_fma(-D[31], m, L[17]);
+      L[18] = m2l_fma(-D[32], m, L[18]);
+      L[19] = m2l_fma(-D[33], m, L[19]);
+      L[20] = m2l_fma(D[36], m, L[20]);
+      L[21] = m2l_fma(D[38], m, L[21]);
+      L[22] = m2l_fma(D[39], m, L[22]);
+      L[23] = m2l_fma(D[41], m, L[23]);
+      L[24] = m2l_fma(D[42], m, L[24]);
+      L[25] = m2l_fma(D[43], m, L[25]);
+      L[26] = m2l_fma(D[45], m, L[26]);
+      L[27] = m2l_fma(D[46], m, L[27]);
+      L[28] = m2l_fma(D[47], m, L[28]);
+      L[29] = m2l_fma(D[48], m, L[29]);
+      L[30] = m2l_fma(D[50], m, L[30]);
+      L[31] = m2l_fma(D[51], m, L[31]);
+      L[32] = m2l_fma(D[52], m, L[32]);
+      L[33] = m2l_fma(D[53], m, L[33]);
+      L[34] = m2l_fma(D[54], m, L[34]);
+      L[35] = m2l_fma(-D[57], m, L[35]);
+      L[36] = m2l_fma(-D[59], m, L[36]);
+      L[37] = m2l_fma(-D[60], m, L[37]);
+      L[38] = m2l_fma(-D[62], m, L[38]);
+      L[39] = m2l_fma(-D[63], m, L[39]);
+      L[40] = m2l_fma(-D[64], m, L[40]);
+      L[41] = m2l_fma(-D[66], m, L[41]);
+      L[42] = m2l_fma(-D[67], m, L[42]);
+      L[43] = m2l_fma(-D[68], m, L[43]);
+      L[44] = m2l_fma(-D[69], m, L[44]);
+      L[45] = m2l_fma(-D[71], m, L[45]);
+      L[46] = m2l_fma(-D[72], m, L[46]);
+      L[47] = m2l_fma(-D[73], m, L[47]);
+      L[48] = m2l_fma(-D[74], m, L[48]);
+      L[49] = m2l_fma(-D[75], m, L[49]);
+      L[50] = m2l_fma(-D[77], m, L[50]);
+      L[51] = m2l_fma(-D[78], m, L[51]);
+      L[52] = m2l_fma(-D[79], m, L[52]);
+      L[53] = m2l_fma(-D[80], m, L[53]);
+      L[54] = m2l_fma(-D[81], m, L[54]);
+      L[55] = m2l_fma(-D[82], m, L[55]);
     }
-    { const float m = __ldg(Ms + 3);
-      L[1] = fmaf(-D[6], m, L[1]);
-      L[2] = fmaf(-D[8], m, L[2]);
-      L[3] = fmaf(-D[9], m, L[3]);
-      L[4] = fmaf(D[12], m, L[4]);
-      L[5] = fmaf(D[14], m, L[5]);
-      L[6] = fmaf(D[15], m, L[6]);
-      L[7] = fmaf(D[17], m, L[7]);
-      L[8] = fmaf(D[18], m, L[8]);
-      L[9] = fmaf(D[19], m, L[9]);
-      L[10] = fmaf(-D[22], m, L[10]);
-      L[11] = fmaf(-D[24], m, L[11]);
-      L[12] = fmaf(-D[25], m, L[12]);
-      L[13] = fmaf(-D[27], m, L[13]);
-      L[14] = fmaf(-D[28], m, L[14]);
-      L[15] = fmaf(-D[29], m, L[15]);
-      L[16] = fmaf(-D[31], m, L[16]);
-      L[17] = fmaf(-D[32], m, L[17]);
-      L[18] = fmaf(-D[33], m, L[18]);
-      L[19] = fmaf(-D[34], m, L[19]);
-      L[20] = fmaf(D[37], m, L[20]);
-      L[21] = fmaf(D[39], m, L[21]);
-      L[22] = fmaf(D[40], m, L[22]);
-      L[23] = fmaf(D[42], m, L[23]);
-      L[24] = fmaf(D[43], m, L[24]);
-      L[25] = fmaf(D[44], m, L[25]);
-      L[26] = fmaf(D[46], m, L[26]);
-      L[27] = fmaf(D[47], m, L[27]);
-      L[28] = fmaf(D[48], m, L[28]);
-      L[29] = fmaf(D[49], m, L[29]);
-      L[30] = fmaf(D[51], m, L[30]);
-      L[31] = fmaf(D[52], m, L[31]);
-      L[32] = fmaf(D[53], m, L[32]);
-      L[33] = fmaf(D[54], m, L[33]);
-      L[34] = fmaf(D[55], m, L[34]);
-      L[35] = fmaf(-D[58], m, L[35]);
-      L[36] = fmaf(-D[60], m, L[36]);
-      L[37] = fmaf(-D[61], m, L[37]);
-      L[38] = fmaf(-D[63], m, L[38]);
-      L[39] = fmaf(-D[64], m, L[39]);
-      L[40] = fmaf(-D[65], m, L[40]);
-      L[41] = fmaf(-D[67], m, L[41]);
-      L[42] = fmaf(-D[68], m, L[42]);
-      L[43] = fmaf(-D[69], m, L[43]);
-      L[44] = fmaf(-D[70], m, L[44]);
-      L[45] = fmaf(-D[72], m, L[45]);
-      L[46] = fmaf(-D[73], m, L[46]);
-      L[47] = fmaf(-D[74], m, L[47]);
-      L[48] = fmaf(-D[75], m, L[48]);
-      L[49] = fmaf(-D[76], m, L[49]);
-      L[50] = fmaf(-D[78], m, L[50]);
-      L[51] = fmaf(-D[79], m, L[51]);
-      L[52] = fmaf(-D[80], m, L[52]);
-      L[53] = fmaf(-D[81], m, L[53]);
-      L[54] = fmaf(-D[82], m, L[54]);
-      L[55] = fmaf(-D[83], m, L[55]);
+    { const T m = __ldg(Ms + 3);
+      L[1] = m2l_fma(-D[6], m, L[1]);
+      L[2] = m2l_fma(-D[8], m, L[2]);
+      L[3] = m2l_fma(-D[9], m, L[3]);
+      L[4] = m2l_fma(D[12], m, L[4]);
+      L[5] = m2l_fma(D[14], m, L[5]);
+      L[6] = m2l_fma(D[15], m, L[6]);
+      L[7] = m2l_fma(D[17], m, L[7]);
+      L[8] = m2l_fma(D[18], m, L[8]);
+      L[9] = m2l_fma(D[19], m, L[9]);
+      L[10] = m2l_fma(-D[22], m, L[10]);
+      L[11] = m2l_fma(-D[24], m, L[11]);
+      L[12] = m2l_fma(-D[25], m, L[12]);
+      L[13] = m2l_fma(-D[27], m, L[13]);
+      L[14] = m2l_fma(-D[28], m, L[14]);
+      L[15] = m2l_fma(-D[29], m, L[15]);
+      L[16] = m2l_fma(-D[31], m, L[16]);
+      L[17] = m2l_fma(-D[32], m, L[17]);
+      L[18] = m2l_fma(-D[33], m, L[18]);
+      L[19] = m2l_fma(-D[34], m, L[19]);
+      L[20] = m2l_fma(D[37], m, L[20]);
+      L[21] = m2l_fma(D[39], m, L[21]);
+      L[22] = m2l_fma(D[40], m, L[22]);
+      L[23] = m2l_fma(D[42], m, L[23]);
+      L[24] = m2l_fma(D[43], m, L[24]);
+      L[25] = m2l_fma(D[44], m, L[25]);
+      L[26] = m2l_fma(D[46], m, L[26]);
+      L[27] = m2l_fma(D[47], m, L[27]);
+      L[28] = m2l_fma(D[48], m, L[28]);
+      L[29] = m2l_fma(D[49], m, L[29]);
+      L[30] = m2l_fma(D[51], m, L[30]);
+      L[31] = m2l_fma(D[52], m, L[31]);
+      L[32] = m2l_fma(D[53], m, L[32]);
+      L[33] = m2l_fma(D[54], m, L[33]);
+      L[34] = m2l_fma(D[55], m, L[34]);
+      L[35] = m2l_fma(-D[58], m, L[35]);
+      L[36] = m2l_fma(-D[60], m, L[36]);
+      L[37] = m2l_fma(-D[61], m, L[37]);
+      L[38] = m2l_fma(-D[63], m, L[38]);
+      L[39] = m2l_fma(-D[64], m, L[39]);
+      L[40] = m2l_fma(-D[65], m, L[40]);
+      L[41] = m2l_fma(-D[67], m, L[41]);
+      L[42] = m2l_fma(-D[68], m, L[42]);
+      L[43] = m2l_fma(-D[69], m, L[43]);
+      L[44] = m2l_fma(-D[70], m, L[44]);
+      L[45] = m2l_fma(-D[72], m, L[45]);
+      L[46] = m2l_fma(-D[73], m, L[46]);
+      L[47] = m2l_fma(-D[74], m, L[47]);
+      L[48] = m2l_fma(-D[75], m, L[48]);
+      L[49] = m2l_fma(-D[76], m, L[49]);
+      L[50] = m2l_fma(-D[78], m, L[50]);
+      L[51] = m2l_fma(-D[79], m, L[51]);
+      L[52] = m2l_fma(-D[80], m, L[52]);
+      L[53] = m2l_fma(-D[81], m, L[53]);
+      L[54] = m2l_fma(-D[82], m, L[54]);
+      L[55] = m2l_fma(-D[83], m, L[55]);
     }
-    { const float m = __ldg(Ms + 4);
-      L[1] = fmaf(-D[10], m, L[1]);
-      L[2] = fmaf(-D[11], m, L[2]);
-      L[3] = fmaf(-D[12], m, L[3]);
-      L[4] = fmaf(D[20], m, L[4]);
-      L[5] = fmaf(D[21], m, L[5]);
-      L[6] = fmaf(D[22], m, L[6]);
-      L[7] = fmaf(D[23], m, L[7]);
-      L[8] = fmaf(D[24], m, L[8]);
-      L[9] = fmaf(D[25], m, L[9]);
-      L[10] = fmaf(-D[35], m, L[10]);
-      L[11] = fmaf(-D[36], m, L[11]);
-      L[12] = fmaf(-D[37], m, L[12]);
-      L[13] = fmaf(-D[38], m, L[13]);
-      L[14] = fmaf(-D[39], m, L[14]);
-      L[15] = fmaf(-D[40], m, L[15]);
-      L[16] = fmaf(-D[41], m, L[16]);
-      L[17] = fmaf(-D[42], m, L[17]);
-      L[18] = fmaf(-D[43], m, L[18]);
-      L[19] = fmaf(-D[44], m, L[19]);
-      L[20] = fmaf(D[56], m, L[20]);
-      L[21] = fmaf(D[57], m, L[21]);
-      L[22] = fmaf(D[58], m, L[22]);
-      L[23] = fmaf(D[59], m, L[23]);
-      L[24] = fmaf(D[60], m, L[24]);
-      L[25] = fmaf(D[61], m, L[25]);
-      L[26] = fmaf(D[62], m, L[26]);
-      L[27] = fmaf(D[63], m, L[27]);
-      L[28] = fmaf(D[64], m, L[28]);
-      L[29] = fmaf(D[65], m, L[29]);
-      L[30] = fmaf(D[66], m, L[30]);
-      L[31] = fmaf(D[67], m, L[31]);
-      L[32] = fmaf(D[68], m, L[32]);
-      L[33] = fmaf(D[69], m, L[33]);
-      L[34] = fmaf(D[70], m, L[34]);
+    { const T m = __ldg(Ms + 4);
+      L[1] = m2l_fma(-D[10], m, L[1]);
+      L[2] = m2l_fma(-D[11], m, L[2]);
+      L[3] = m2l_fma(-D[12], m, L[3]);
+      L[4] = m2l_fma(D[20], m, L[4]);
+      L[5] = m2l_fma(D[21], m, L[5]);
+      L[6] = m2l_fma(D[22], m, L[6]);
+      L[7] = m2l_fma(D[23], m, L[7]);
+      L[8] = m2l_fma(D[24], m, L[8]);
+      L[9] = m2l_fma(D[25], m, L[9]);
+      L[10] = m2l_fma(-D[35], m, L[10]);
+      L[11] = m2l_fma(-D[36], m, L[11]);
+      L[12] = m2l_fma(-D[37], m, L[12]);
+      L[13] = m2l_fma(-D[38], m, L[13]);
+      L[14] = m2l_fma(-D[39], m, L[14]);
+      L[15] = m2l_fma(-D[40], m, L[15]);
+      L[16] = m2l_fma(-D[41], m, L[16]);
+      L[17] = m2l_fma(-D[42], m, L[17]);
+      L[18] = m2l_fma(-D[43], m, L[18]);
+      L[19] = m2l_fma(-D[44], m, L[19]);
+      L[20] = m2l_fma(D[56], m, L[20]);
+      L[21] = m2l_fma(D[57], m, L[21]);
+      L[22] = m2l_fma(D[58], m, L[22]);
+      L[23] = m2l_fma(D[59], m, L[23]);
+      L[24] = m2l_fma(D[60], m, L[24]);
+      L[25] = m2l_fma(D[61], m, L[25]);
+      L[26] = m2l_fma(D[62], m, L[26]);
+      L[27] = m2l_fma(D[63], m, L[27]);
+      L[28] = m2l_fma(D[64], m, L[28]);
+      L[29] = m2l_fma(D[65], m, L[29]);
+      L[30] = m2l_fma(D[66], m, L[30]);
+      L[31] = m2l_fma(D[67], m, L[31]);
+      L[32] = m2l_fma(D[68], m, L[32]);
+      L[33] = m2l_fma(D[69], m, L[33]);
+      L[34] = m2l_fma(D[70], m, L[34]);
     }
-    { const float m = __ldg(Ms + 5);
-      L[1] = fmaf(-D[11], m, L[1]);
-      L[2] = fmaf(-D[13], m, L[2]);
-      L[3] = fmaf(-D[14], m, L[3]);
-      L[4] = fmaf(D[21], m, L[4]);
-      L[5] = fmaf(D[23], m, L[5]);
-      L[6] = fmaf(D[24], m, L[6]);
-      L[7] = fmaf(D[26], m, L[7]);
-      L[8] = fmaf(D[27], m, L[8]);
-      L[9] = fmaf(D[28], m, L[9]);
-      L[10] = fmaf(-D[36], m, L[10]);
-      L[11] = fmaf(-D[38], m, L[11]);
-      L[12] = fmaf(-D[39], m, L[12]);
-      L[13] = fmaf(-D[41], m, L[13]);
-      L[14] = fmaf(-D[42], m, L[14]);
-      L[15] = fmaf(-D[43], m, L[15]);
-      L[16] = fmaf(-D[45], m, L[16]);
-      L[17] = fmaf(-D[46], m, L[17]);
-      L[18] = fmaf(-D[47], m, L[18]);
-      L[19] = fmaf(-D[48], m, L[19]);
-      L[20] = fmaf(D[57], m, L[20]);
-      L[21] = fmaf(D[59], m, L[21]);
-      L[22] = fmaf(D[60], m, L[22]);
-      L[23] = fmaf(D[62], m, L[23]);
-      L[24] = fmaf(D[63], m, L[24]);
-      L[25] = fmaf(D[64], m, L[25]);
-      L[26] = fmaf(D[66], m, L[26]);
-      L[27] = fmaf(D[67], m, L[27]);
-      L[28] = fmaf(D[68], m, L[28]);
-      L[29] = fmaf(D[69], m, L[29]);
-      L[30] = fmaf(D[71], m, L[30]);
-      L[31] = fmaf(D[72], m, L[31]);
-      L[32] = fmaf(D[73], m, L[32]);
-      L[33] = fmaf(D[74], m, L[33]);
-      L[34] = fmaf(D[75], m, L[34]);
+    { const T m = __ldg(Ms + 5);
+      L[1] = m2l_fma(-D[11], m, L[1]);
+      L[2] = m2l_fma(-D[13], m, L[2]);
+      L[3] = m2l_fma(-D[14], m, L[3]);
+      L[4] = m2l_fma(D[21], m, L[4]);
+      L[5] = m2l_fma(D[23], m, L[5]);
+      L[6] = m2l_fma(D[24], m, L[6]);
+      L[7] = m2l_fma(D[26], m, L[7]);
+      L[8] = m2l_fma(D[27], m, L[8]);
+      L[9] = m2l_fma(D[28], m, L[9]);
+      L[10] = m2l_fma(-D[36], m, L[10]);
+      L[11] = m2l_fma(-D[38], m, L[11]);
+      L[12] = m2l_fma(-D[39], m, L[12]);
+      L[13] = m2l_fma(-D[41], m, L[13]);
+      L[14] = m2l_fma(-D[42], m, L[14]);
+      L[15] = m2l_fma(-D[43], m, L[15]);
+      L[16] = m2l_fma(-D[45], m, L[16]);
+      L[17] = m2l_fma(-D[46], m, L[17]);
+      L[18] = m2l_fma(-D[47], m, L[18]);
+      L[19] = m2l_fma(-D[48], m, L[19]);
+      L[20] = m2l_fma(D[57], m, L[20]);
+      L[21] = m2l_fma(D[59], m, L[21]);
+      L[22] = m2l_fma(D[60], m, L[22]);
+      L[23] = m2l_fma(D[62], m, L[23]);
+      L[24] = m2l_fma(D[63], m, L[24]);
+      L[25] = m2l_fma(D[64], m, L[25]);
+      L[26] = m2l_fma(D[66], m, L[26]);
+      L[27] = m2l_fma(D[67], m, L[27]);
+      L[28] = m2l_fma(D[68], m, L[28]);
+      L[29] = m2l_fma(D[69], m, L[29]);
+      L[30] = m2l_fma(D[71], m, L[30]);
+      L[31] = m2l_fma(D[72], m, L[31]);
+      L[32] = m2l_fma(D[73], m, L[32]);
+      L[33] = m2l_fma(D[74], m, L[33]);
+      L[34] = m2l_fma(D[75], m, L[34]);
     }
-    { const float m = __ldg(Ms + 6);
-      L[1] = fmaf(-D[12], m, L[1]);
-      L[2] = fmaf(-D[14], m, L[2]);
-      L[3] = fmaf(-D[15], m, L[3]);
-      L[4] = fmaf(D[22], m, L[4]);
-      L[5] = fmaf(D[24], m, L[5]);
-      L[6] = fmaf(D[25], m, L[6]);
-      L[7] = fmaf(D[27], m, L[7]);
-      L[8] = fmaf(D[28], m, L[8]);
-      L[9] = fmaf(D[29], m, L[9]);
-      L[10] = fmaf(-D[37], m, L[10]);
-      L[11] = fmaf(-D[39], m, L[11]);
-      L[12] = fmaf(-D[40], m, L[12]);
-      L[13] = fmaf(-D[42], m, L[13]);
-      L[14] = fmaf(-D[43], m, L[14]);
-      L[15] = fmaf(-D[44], m, L[15]);
-      L[16] = fmaf(-D[46], m, L[16]);
-      L[17] = fmaf(-D[47], m, L[17]);
-      L[18] = fmaf(-D[48], m, L[18]);
-      L[19] = fmaf(-D[49], m, L[19]);
-      L[20] = fmaf(D[58], m, L[20]);
-      L[21] = fmaf(D[60], m, L[21]);
-      L[22] = fmaf(D[61], m, L[22]);
-      L[23] = fmaf(D[63], m, L[23]);
-      L[24] = fmaf(D[64], m, L[24]);
-      L[25] = fmaf(D[65], m, L[25]);
-      L[26] = fmaf(D[67], m, L[26]);
-      L[27] = fmaf(D[68], m, L[27]);
-      L[28] = fmaf(D[69], m, L[28]);
-      L[29] = fmaf(D[70], m, L[29]);
-      L[30] = fmaf(D[72], m, L[30]);
-      L[31] = fmaf(D[73], m, L[31]);
-      L[32] = fmaf(D[74], m, L[32]);
-      L[33] = fmaf(D[75], m, L[33]);
-      L[34] = fmaf(D[76], m, L[34]);
+    { const T m = __ldg(Ms + 6);
+      L[1] = m2l_fma(-D[12], m, L[1]);
+      L[2] = m2l_fma(-D[14], m, L[2]);
+      L[3] = m2l_fma(-D[15], m, L[3]);
+      L[4] = m2l_fma(D[22], m, L[4]);
+      L[5] = m2l_fma(D[24], m, L[5]);
+      L[6] = m2l_fma(D[25], m, L[6]);
+      L[7] = m2l_fma(D[27], m, L[7]);
+      L[8] = m2l_fma(D[28], m, L[8]);
+      L[9] = m2l_fma(D[29], m, L[9]);
+      L[10] = m2l_fma(-D[37], m, L[10]);
+      L[11] = m2l_fma(-D[39], m, L[11]);
+      L[12] = m2l_fma(-D[40], m, L[12]);
+      L[13] = m2l_fma(-D[42], m, L[13]);
+      L[14] = m2l_fma(-D[43], m, L[14]);
+      L[15] = m2l_fma(-D[44], m, L[15]);
+      L[16] = m2l_fma(-D[46], m, L[16]);
+      L[17] = m2l_fma(-D[47], m, L[17]);
+      L[18] = m2l_fma(-D[48], m, L[18]);
+      L[19] = m2l_fma(-D[49], m, L[19]);
+      L[20] = m2l_fma(D[58], m, L[20]);
+      L[21] = m2l_fma(D[60], m, L[21]);
+      L[22] = m2l_fma(D[61], m, L[22]);
+      L[23] = m2l_fma(D[63], m, L[23]);
+      L[24] = m2l_fma(D[64], m, L[24]);
+      L[25] = m2l_fma(D[65], m, L[25]);
+      L[26] = m2l_fma(D[67], m, L[26]);
+      L[27] = m2l_fma(D[68], m, L[27]);
+      L[28] = m2l_fma(D[69], m, L[28]);
+      L[29] = m2l_fma(D[70], m, L[29]);
+      L[30] = m2l_fma(D[72], m, L[30]);
+      L[31] = m2l_fma(D[73], m, L[31]);
+      L[32] = m2l_fma(D[74], m, L[32]);
+      L[33] = m2l_fma(D[75], m, L[33]);
+      L[34] = m2l_fma(D[76], m, L[34]);
     }
-    { const float m = __ldg(Ms + 7);
-      L[1] = fmaf(-D[13], m, L[1]);
-      L[2] = fmaf(-D[16], m, L[2]);
-      L[3] = fmaf(-D[17], m, L[3]);
-      L[4] = fmaf(D[23], m, L[4]);
-      L[5] = fmaf(D[26], m, L[5]);
-      L[6] = fmaf(D[27], m, L[6]);
-      L[7] = fmaf(D[30], m, L[7]);
-      L[8] = fmaf(D[31], m, L[8]);
-      L[9] = fmaf(D[32], m, L[9]);
-      L[10] = fmaf(-D[38], m, L[10]);
-      L[11] = fmaf(-D[41], m, L[11]);
-      L[12] = fmaf(-D[42], m, L[12]);
-      L[13] = fmaf(-D[45], m, L[13]);
-      L[14] = fmaf(-D[46], m, L[14]);
-      L[15] = fmaf(-D[47], m, L[15]);
-      L[16] = fmaf(-D[50], m, L[16]);
-      L[17] = fmaf(-D[51], m, L[17]);
-      L[18] = fmaf(-D[52], m, L[18]);
-      L[19] = fmaf(-D[53], m, L[19]);
-      L[20] = fmaf(D[59], m, L[20]);
-      L[21] = fmaf(D[62], m, L[21]);
-      L[22] = fmaf(D[63], m, L[22]);
-      L[23] = fmaf(D[66], m, L[23]);
-      L[24] = fmaf(D[67], m, L[24]);
-      L[25] = fmaf(D[68], m, L[25]);
-      L[26] = fmaf(D[71], m, L[26]);
-      L[27] = fmaf(D[72], m, L[27]);
-      L[28] = fmaf(D[73], m, L[28]);
-      L[29] = fmaf(D[74], m, L[29]);
-      L[30] = fmaf(D[77], m, L[30]);
-      L[31] = fmaf(D[78], m, L[31]);
-      L[32] = fmaf(D[79], m, L[32]);
-      L[33] = fmaf(D[80], m, L[33]);
-      L[34] = fmaf(D[81], m, L[34]);
+    { const T m = __ldg(Ms + 7);
+      L[1] = m2l_fma(-D[13], m, L[1]);
+      L[2] = m2l_fma(-D[16], m, L[2]);
+      L[3] = m2l_fma(-D[17], m, L[3]);
+      L[4] = m2l_fma(D[23], m, L[4]);
+      L[5] = m2l_fma(D[26], m, L[5]);
+      L[6] = m2l_fma(D[27], m, L[6]);
+      L[7] = m2l_fma(D[30], m, L[7]);
+      L[8] = m2l_fma(D[31], m, L[8]);
+      L[9] = m2l_fma(D[32], m, L[9]);
+      L[10] = m2l_fma(-D[38], m, L[10]);
+      L[11] = m2l_fma(-D[41], m, L[11]);
+      L[12] = m2l_fma(-D[42], m, L[12]);
+      L[13] = m2l_fma(-D[45], m, L[13]);
+      L[14] = m2l_fma(-D[46], m, L[14]);
+      L[15] = m2l_fma(-D[47], m, L[15]);
+      L[16] = m2l_fma(-D[50], m, L[16]);
+      L[17] = m2l_fma(-D[51], m, L[17]);
+      L[18] = m2l_fma(-D[52], m, L[18]);
+      L[19] = m2l_fma(-D[53], m, L[19]);
+      L[20] = m2l_fma(D[59], m, L[20]);
+      L[21] = m2l_fma(D[62], m, L[21]);
+      L[22] = m2l_fma(D[63], m, L[22]);
+      L[23] = m2l_fma(D[66], m, L[23]);
+      L[24] = m2l_fma(D[67], m, L[24]);
+      L[25] = m2l_fma(D[68], m, L[25]);
+      L[26] = m2l_fma(D[71], m, L[26]);
+      L[27] = m2l_fma(D[72], m, L[27]);
+      L[28] = m2l_fma(D[73], m, L[28]);
+      L[29] = m2l_fma(D[74], m, L[29]);
+      L[30] = m2l_fma(D[77], m, L[30]);
+      L[31] = m2l_fma(D[78], m, L[31]);
+      L[32] = m2l_fma(D[79], m, L[32]);
+      L[33] = m2l_fma(D[80], m, L[33]);
+      L[34] = m2l_fma(D[81], m, L[34]);
     }
-    { const float m = __ldg(Ms + 8);
-      L[1] = fmaf(-D[14], m, L[1]);
-      L[2] = fmaf(-D[17], m, L[2]);
-      L[3] = fmaf(-D[18], m, L[3]);
-      L[4] = fmaf(D[24], m, L[4]);
-      L[5] = fmaf(D[27], m, L[5]);
-      L[6] = fmaf(D[28], m, L[6]);
-      L[7] = fmaf(D[31], m, L[7]);
-      L[8] = fmaf(D[32], m, L[8]);
-      L[9] = fmaf(D[33], m, L[9]);
-      L[10] = fmaf(-D[39], m, L[10]);
-      L[11] = fmaf(-D[42], m, L[11]);
-      L[12] = fmaf(-D[43], m, L[12]);
-      L[13] = fmaf(-D[46], m, L[13]);
-      L[14] = fmaf(-D[47], m, L[14]);
-      L[15] = fmaf(-D[48], m, L[15]);
-      L[16] = fmaf(-D[51], m, L[16]);
-      L[17] = fmaf(-D[52], m, L[17]);
-      L[18] = fmaf(-D[53], m, L[18]);
-      L[19] = fmaf(-D[54], m, L[19]);
-      L[20] = fmaf(D[60], m, L[20]);
-      L[21] = fmaf(D[63], m, L[21]);
-      L[22] = fmaf(D[64], m, L[22]);
-      L[23] = fmaf(D[67], m, L[23]);
-      L[24] = fmaf(D[68], m, L[24]);
-      L[25] = fmaf(D[69], m, L[25]);
-      L[26] = fmaf(D[72], m, L[26]);
-      L[27] = fmaf(D[73], m, L[27]);
-      L[28] = fmaf(D[74], m, L[28]);
-      L[29] = fmaf(D[75], m, L[29]);
-      L[30] = fmaf(D[78], m, L[30]);
-      L[31] = fmaf(D[79], m, L[31]);
-      L[32] = fmaf(D[80], m, L[32]);
-      L[33] = fmaf(D[81], m, L[33]);
-      L[34] = fmaf(D[82], m, L[34]);
+    { const T m = __ldg(Ms + 8);
+      L[1] = m2l_fma(-D[14], m, L[1]);
+      L[2] = m2l_fma(-D[17], m, L[2]);
+      L[3] = m2l_fma(-D[18], m, L[3]);
+      L[4] = m2l_fma(D[24], m, L[4]);
+      L[5] = m2l_fma(D[27], m, L[5]);
+      L[6] = m2l_fma(D[28], m, L[6]);
+      L[7] = m2l_fma(D[31], m, L[7]);
+      L[8] = m2l_fma(D[32], m, L[8]);
+      L[9] = m2l_fma(D[33], m, L[9]);
+      L[10] = m2l_fma(-D[39], m, L[10]);
+      L[11] = m2l_fma(-D[42], m, L[11]);
+      L[12] = m2l_fma(-D[43], m, L[12]);
+      L[13] = m2l_fma(-D[46], m, L[13]);
+      L[14] = m2l_fma(-D[47], m, L[14]);
+      L[15] = m2l_fma(-D[48], m, L[15]);
+      L[16] = m2l_fma(-D[51], m, L[16]);
+      L[17] = m2l_fma(-D[52], m, L[17]);
+      L[18] = m2l_fma(-D[53], m, L[18]);
+      L[19] = m2l_fma(-D[54], m, L[19]);
+      L[20] = m2l_fma(D[60], m, L[20]);
+      L[21] = m2l_fma(D[63], m, L[21]);
+      L[22] = m2l_fma(D[64], m, L[22]);
+      L[23] = m2l_fma(D[67], m, L[23]);
+      L[24] = m2l_fma(D[68], m, L[24]);
+      L[25] = m2l_fma(D[69], m, L[25]);
+      L[26] = m2l_fma(D[72], m, L[26]);
+      L[27] = m2l_fma(D[73], m, L[27]);
+      L[28] = m2l_fma(D[74], m, L[28]);
+      L[29] = m2l_fma(D[75], m, L[29]);
+      L[30] = m2l_fma(D[78], m, L[30]);
+      L[31] = m2l_fma(D[79], m, L[31]);
+      L[32] = m2l_fma(D[80], m, L[32]);
+      L[33] = m2l_fma(D[81], m, L[33]);
+      L[34] = m2l_fma(D[82], m, L[34]);
     }
-    { const float m = __ldg(Ms + 9);
-      L[1] = fmaf(-D[15], m, L[1]);
-      L[2] = fmaf(-D[18], m, L[2]);
-      L[3] = fmaf(-D[19], m, L[3]);
-      L[4] = fmaf(D[25], m, L[4]);
-      L[5] = fmaf(D[28], m, L[5]);
-      L[6] = fmaf(D[29], m, L[6]);
-      L[7] = fmaf(D[32], m, L[7]);
-      L[8] = fmaf(D[33], m, L[8]);
-      L[9] = fmaf(D[34], m, L[9]);
-      L[10] = fmaf(-D[40], m, L[10]);
-      L[11] = fmaf(-D[43], m, L[11]);
-      L[12] = fmaf(-D[44], m, L[12]);
-      L[13] = fmaf(-D[47], m, L[13]);
-      L[14] = fmaf(-D[48], m, L[14]);
-      L[15] = fmaf(-D[49], m, L[15]);
-      L[16] = fmaf(-D[52], m, L[16]);
-      L[17] = fmaf(-D[53], m, L[17]);
-      L[18] = fmaf(-D[54], m, L[18]);
-      L[19] = fmaf(-D[55], m, L[19]);
-      L[20] = fmaf(D[61], m, L[20]);
-      L[21] = fmaf(D[64], m, L[21]);
-      L[22] = fmaf(D[65], m, L[22]);
-      L[23] = fmaf(D[68], m, L[23]);
-      L[24] = fmaf(D[69], m, L[24]);
-      L[25] = fmaf(D[70], m, L[25]);
-      L[26] = fmaf(D[73], m, L[26]);
-      L[27] = fmaf(D[74], m, L[27]);
-      L[28] = fmaf(D[75], m, L[28]);
-      L[29] = fmaf(D[76], m, L[29]);
-      L[30] = fmaf(D[79], m, L[30]);
-      L[31] = fmaf(D[80], m, L[31]);
-      L[32] = fmaf(D[81], m, L[32]);
-      L[33] = fmaf(D[82], m, L[33]);
-      L[34] = fmaf(D[83], m, L[34]);
+    { const T m = __ldg(Ms + 9);
+      L[1] = m2l_fma(-D[15], m, L[1]);
+      L[2] = m2l_fma(-D[18], m, L[2]);
+      L[3] = m2l_fma(-D[19], m, L[3]);
+      L[4] = m2l_fma(D[25], m, L[4]);
+      L[5] = m2l_fma(D[28], m, L[5]);
+      L[6] = m2l_fma(D[29], m, L[6]);
+      L[7] = m2l_fma(D[32], m, L[7]);
+      L[8] = m2l_fma(D[33], m, L[8]);
+      L[9] = m2l_fma(D[34], m, L[9]);
+      L[10] = m2l_fma(-D[40], m, L[10]);
+      L[11] = m2l_fma(-D[43], m, L[11]);
+      L[12] = m2l_fma(-D[44], m, L[12]);
+      L[13] = m2l_fma(-D[47], m, L[13]);
+      L[14] = m2l_fma(-D[48], m, L[14]);
+      L[15] = m2l_fma(-D[49], m, L[15]);
+      L[16] = m2l_fma(-D[52], m, L[16]);
+      L[17] = m2l_fma(-D[53], m, L[17]);
+      L[18] = m2l_fma(-D[54], m, L[18]);
+      L[19] = m2l_fma(-D[55], m, L[19]);
+      L[20] = m2l_fma(D[61], m, L[20]);
+      L[21] = m2l_fma(D[64], m, L[21]);
+      L[22] = m2l_fma(D[65], m, L[22]);
+      L[23] = m2l_fma(D[68], m, L[23]);
+      L[24] = m2l_fma(D[69], m, L[24]);
+      L[25] = m2l_fma(D[70], m, L[25]);
+      L[26] = m2l_fma(D[73], m, L[26]);
+      L[27] = m2l_fma(D[74], m, L[27]);
+      L[28] = m2l_fma(D[75], m, L[28]);
+      L[29] = m2l_fma(D[76], m, L[29]);
+      L[30] = m2l_fma(D[79], m, L[30]);
+      L[31] = m2l_fma(D[80], m, L[31]);
+      L[32] = m2l_fma(D[81], m, L[32]);
+      L[33] = m2l_fma(D[82], m, L[33]);
+      L[34] = m2l_fma(D[83], m, L[34]);
     }
-    { const float m = __ldg(Ms + 10);
-      L[1] = fmaf(-D[20], m, L[1]);
-      L[2] = fmaf(-D[21], m, L[2]);
-      L[3] = fmaf(-D[22], m, L[3]);
-      L[4] = fmaf(D[35], m, L[4]);
-      L[5] = fmaf(D[36], m, L[5]);
-      L[6] = fmaf(D[37], m, L[6]);
-      L[7] = fmaf(D[38], m, L[7]);
-      L[8] = fmaf(D[39], m, L[8]);
-      L[9] = fmaf(D[40], m, L[9]);
-      L[10] = fmaf(-D[56], m, L[10]);
-      L[11] = fmaf(-D[57], m, L[11]);
-      L[12] = fmaf(-D[58], m, L[12]);
-      L[13] = fmaf(-D[59], m, L[13]);
-      L[14] = fmaf(-D[60], m, L[14]);
-      L[15] = fmaf(-D[61], m, L[15]);
-      L[16] = fmaf(-D[62], m, L[16]);
-      L[17] = fmaf(-D[63], m, L[17]);
-      L[18] = fmaf(-D[64], m, L[18]);
-      L[19] = fmaf(-D[65], m, L[19]);
+    { const T m = __ldg(Ms + 10);
+      L[1] = m2l_fma(-D[20], m, L[1]);
+      L[2] = m2l_fma(-D[21], m, L[2]);
+      L[3] = m2l_fma(-D[22], m, L[3]);
+      L[4] = m2l_fma(D[35], m, L[4]);
+      L[5] = m2l_fma(D[36], m, L[5]);
+      L[6] = m2l_fma(D[37], m, L[6]);
+      L[7] = m2l_fma(D[38], m, L[7]);
+      L[8] = m2l_fma(D[39], m, L[8]);
+      L[9] = m2l_fma(D[40], m, L[9]);
+      L[10] = m2l_fma(-D[56], m, L[10]);
+      L[11] = m2l_fma(-D[57], m, L[11]);
+      L[12] = m2l_fma(-D[58], m, L[12]);
+      L[13] = m2l_fma(-D[59], m, L[13]);
+      L[14] = m2l_fma(-D[60], m, L[14]);
+      L[15] = m2l_fma(-D[61], m, L[15]);
+      L[16] = m2l_fma(-D[62], m, L[16]);
+      L[17] = m2l_fma(-D[63], m, L[17]);
+      L[18] = m2l_fma(-D[64], m, L[18]);
+      L[19] = m2l_fma(-D[65], m, L[19]);
     }
-    { const float m = __ldg(Ms + 11);
-      L[1] = fmaf(-D[21], m, L[1]);
-      L[2] = fmaf(-D[23], m, L[2]);
-      L[3] = fmaf(-D[24], m, L[3]);
-      L[4] = fmaf(D[36], m, L[4]);
-      L[5] = fmaf(D[38], m, L[5]);
-      L[6] = fmaf(D[39], m, L[6]);
-      L[7] = fmaf(D[41], m, L[7]);
-      L[8] = fmaf(D[42], m, L[8]);
-      L[9] = fmaf(D[43], m, L[9]);
-      L[10] = fmaf(-D[57], m, L[10]);
-      L[11] = fmaf(-D[59], m, L[11]);
-      L[12] = fmaf(-D[60], m, L[12]);
-      L[13] = fmaf(-D[62], m, L[13]);
-      L[14] = fmaf(-D[63], m, L[14]);
-      L[15] = fmaf(-D[64], m, L[15]);
-      L[16] = fmaf(-D[66], m, L[16]);
-      L[17] = fmaf(-D[67], m, L[17]);
-      L[18] = fmaf(-D[68], m, L[18]);
-      L[19] = fmaf(-D[69], m, L[19]);
+    { const T m = __ldg(Ms + 11);
+      L[1] = m2l_fma(-D[21], m, L[1]);
+      L[2] = m2l_fma(-D[23], m, L[2]);
+      L[3] = m2l_fma(-D[24], m, L[3]);
+      L[4] = m2l_fma(D[36], m, L[4]);
+      L[5] = m2l_fma(D[38], m, L[5]);
+      L[6] = m2l_fma(D[39], m, L[6]);
+      L[7] = m2l_fma(D[41], m, L[7]);
+      L[8] = m2l_fma(D[42], m, L[8]);
+      L[9] = m2l_fma(D[43], m, L[9]);
+      L[10] = m2l_fma(-D[57], m, L[10]);
+      L[11] = m2l_fma(-D[59], m, L[11]);
+      L[12] = m2l_fma(-D[60], m, L[12]);
+      L[13] = m2l_fma(-D[62], m, L[13]);
+      L[14] = m2l_fma(-D[63], m, L[14]);
+      L[15] = m2l_fma(-D[64], m, L[15]);
+      L[16] = m2l_fma(-D[66], m, L[16]);
+      L[17] = m2l_fma(-D[67], m, L[17]);
+      L[18] = m2l_fma(-D[68], m, L[18]);
+      L[19] = m2l_fma(-D[69], m, L[19]);
     }
-    { const float m = __ldg(Ms + 12);
-      L[1] = fmaf(-D[22], m, L[1]);
-      L[2] = fmaf(-D[24], m, L[2]);
-      L[3] = fmaf(-D[25], m, L[3]);
-      L[4] = fmaf(D[37], m, L[4]);
-      L[5] = fmaf(D[39], m, L[5]);
-      L[6] = fmaf(D[40], m, L[6]);
-      L[7] = fmaf(D[42], m, L[7]);
-      L[8] = fmaf(D[43], m, L[8]);
-      L[9] = fmaf(D[44], m, L[9]);
-      L[10] = fmaf(-D[58], m, L[10]);
-      L[11] = fmaf(-D[60], m, L[11]);
-      L[12] = fmaf(-D[61], m, L[12]);
-      L[13] = fmaf(-D[63], m, L[13]);
-      L[14] = fmaf(-D[64], m, L[14]);
-      L[15] = fmaf(-D[65], m, L[15]);
-      L[16] = fmaf(-D[67], m, L[16]);
-      L[17] = fmaf(-D[68], m, L[17]);
-      L[18] = fmaf(-D[69], m, L[18]);
-      L[19] = fmaf(-D[70], m, L[19]);
+    { const T m = __ldg(Ms + 12);
+      L[1] = m2l_fma(-D[22], m, L[1]);
+      L[2] = m2l_fma(-D[24], m, L[2]);
+      L[3] = m2l_fma(-D[25], m, L[3]);
+      L[4] = m2l_fma(D[37], m, L[4]);
+      L[5] = m2l_fma(D[39], m, L[5]);
+      L[6] = m2l_fma(D[40], m, L[6]);
+      L[7] = m2l_fma(D[42], m, L[7]);
+      L[8] = m2l_fma(D[43], m, L[8]);
+      L[9] = m2l_fma(D[44], m, L[9]);
+      L[10] = m2l_fma(-D[58], m, L[10]);
+      L[11] = m2l_fma(-D[60], m, L[11]);
+      L[12] = m2l_fma(-D[61], m, L[12]);
+      L[13] = m2l_fma(-D[63], m, L[13]);
+      L[14] = m2l_fma(-D[64], m, L[14]);
+      L[15] = m2l_fma(-D[65], m, L[15]);
+      L[16] = m2l_fma(-D[67], m, L[16]);
+      L[17] = m2l_fma(-D[68], m, L[17]);
+      L[18] = m2l_fma(-D[69], m, L[18]);
+      L[19] = m2l_fma(-D[70], m, L[19]);
     }
-    { const float m = __ldg(Ms + 13);
-      L[1] = fmaf(-D[23], m, L[1]);
-      L[2] = fmaf(-D[26], m, L[2]);
-      L[3] = fmaf(-D[27], m, L[3]);
-      L[4] = fmaf(D[38], m, L[4]);
-      L[5] = fmaf(D[41], m, L[5]);
-      L[6] = fmaf(D[42], m, L[6]);
-      L[7] = fmaf(D[45], m, L[7]);
-      L[8] = fmaf(D[46], m, L[8]);
-      L[9] = fmaf(D[47], m, L[9]);
-      L[10] = fmaf(-D[59], m, L[10]);
-      L[11] = fmaf(-D[62], m, L[11]);
-      L[12] = fmaf(-D[63], m, L[12]);
-      L[13] = fmaf(-D[66], m, L[13]);
-      L[14] = fmaf(-D[67], m, L[14]);
-      L[15] = fmaf(-D[68], m, L[15]);
-      L[16] = fmaf(-D[71], m, L[16]);
-      L[17] = fmaf(-D[72], m, L[17]);
-      L[18] = fmaf(-D[73], m, L[18]);
-      L[19] = fmaf(-D[74], m, L[19]);
+    { const T m = __ldg(Ms + 13);
+      L[1] = m2l_fma(-D[23], m, L[1]);
+      L[2] = m2l_fma(-D[26], m, L[2]);
+      L[3] = m2l_fma(-D[27], m, L[3]);
+      L[4] = m2l_fma(D[38], m, L[4]);
+      L[5] = m2l_fma(D[41], m, L[5]);
+      L[6] = m2l_fma(D[42], m, L[6]);
+      L[7] = m2l_fma(D[45], m, L[7]);
+      L[8] = m2l_fma(D[46], m, L[8]);
+      L[9] = m2l_fma(D[47], m, L[9]);
+      L[10] = m2l_fma(-D[59], m, L[10]);
+      L[11] = m2l_fma(-D[62], m, L[11]);
+      L[12] = m2l_fma(-D[63], m, L[12]);
+      L[13] = m2l_fma(-D[66], m, L[13]);
+      L[14] = m2l_fma(-D[67], m, L[14]);
+      L[15] = m2l_fma(-D[68], m, L[15]);
+      L[16] = m2l_fma(-D[71], m, L[16]);
+      L[17] = m2l_fma(-D[72], m, L[17]);
+      L[18] = m2l_fma(-D[73], m, L[18]);
+      L[19] = m2l_fma(-D[74], m, L[19]);
     }
-    { const float m = __ldg(Ms + 14);
-      L[1] = fmaf(-D[24], m, L[1]);
-      L[2] = fmaf(-D[27], m, L[2]);
-      L[3] = fmaf(-D[28], m, L[3]);
-      L[4] = fmaf(D[39], m, L[4]);
-      L[5] = fmaf(D[42], m, L[5]);
-      L[6] = fmaf(D[43], m, L[6]);
-      L[7] = fmaf(D[46], m, L[7]);
-      L[8] = fmaf(D[47], m, L[8]);
-      L[9] = fmaf(D[48], m, L[9]);
-      L[10] = fmaf(-D[60], m, L[10]);
-      L[11] = fmaf(-D[63], m, L[11]);
-      L[12] = fmaf(-D[64], m, L[12]);
-      L[13] = fmaf(-D[67], m, L[13]);
-      L[14] = fmaf(-D[68], m, L[14]);
-      L[15] = fmaf(-D[69], m, L[15]);
-      L[16] = fmaf(-D[72], m, L[16]);
-      L[17] = fmaf(-D[73], m, L[17]);
-      L[18] = fmaf(-D[74], m, L[18]);
-      L[19] = fmaf(-D[75], m, L[19]);
+    { const T m = __ldg(Ms + 14);
+      L[1] = m2l_fma(-D[24], m, L[1]);
+      L[2] = m2l_fma(-D[27], m, L[2]);
+      L[3] = m2l_fma(-D[28], m, L[3]);
+      L[4] = m2l_fma(D[39], m, L[4]);
+      L[5] = m2l_fma(D[42], m, L[5]);
+      L[6] = m2l_fma(D[43], m, L[6]);
+      L[7] = m2l_fma(D[46], m, L[7]);
+      L[8] = m2l_fma(D[47], m, L[8]);
+      L[9] = m2l_fma(D[48], m, L[9]);
+      L[10] = m2l_fma(-D[60], m, L[10]);
+      L[11] = m2l_fma(-D[63], m, L[11]);
+      L[12] = m2l_fma(-D[64], m, L[12]);
+      L[13] = m2l_fma(-D[67], m, L[13]);
+      L[14] = m2l_fma(-D[68], m, L[14]);
+      L[15] = m2l_fma(-D[69], m, L[15]);
+      L[16] = m2l_fma(-D[72], m, L[16]);
+      L[17] = m2l_fma(-D[73], m, L[17]);
+      L[18] = m2l_fma(-D[74], m, L[18]);
+      L[19] = m2l_fma(-D[75], m, L[19]);
     }
-    { const float m = __ldg(Ms + 15);
-      L[1] = fmaf(-D[25], m, L[1]);
-      L[2] = fmaf(-D[28], m, L[2]);
-      L[3] = fmaf(-D[29], m, L[3]);
-      L[4] = fmaf(D[40], m, L[4]);
-      L[5] = fmaf(D[43], m, L[5]);
-      L[6] = fmaf(D[44], m, L[6]);
-      L[7] = fmaf(D[47], m, L[7]);
-      L[8] = fmaf(D[48], m, L[8]);
-      L[9] = fmaf(D[49], m, L[9]);
-      L[10] = fmaf(-D[61], m, L[10]);
-      L[11] = fmaf(-D[64], m, L[11]);
-      L[12] = fmaf(-D[65], m, L[12]);
-      L[13] = fmaf(-D[68], m, L[13]);
-      L[14] = fmaf(-D[69], m, L[14]);
-      L[15] = fmaf(-D[70], m, L[15]);
-      L[16] = fmaf(-D[73], m, L[16]);
-      L[17] = fmaf(-D[74], m, L[17]);
-      L[18] = fmaf(-D[75], m, L[18]);
-      L[19] = fmaf(-D[76], m, L[19]);
+    { const T m = __ldg(Ms + 15);
+      L[1] = m2l_fma(-D[25], m, L[1]);
+      L[2] = m2l_fma(-D[28], m, L[2]);
+      L[3] = m2l_fma(-D[29], m, L[3]);
+      L[4] = m2l_fma(D[40], m, L[4]);
+      L[5] = m2l_fma(D[43], m, L[5]);
+      L[6] = m2l_fma(D[44], m, L[6]);
+      L[7] = m2l_fma(D[47], m, L[7]);
+      L[8] = m2l_fma(D[48], m, L[8]);
+      L[9] = m2l_fma(D[49], m, L[9]);
+      L[10] = m2l_fma(-D[61], m, L[10]);
+      L[11] = m2l_fma(-D[64], m, L[11]);
+      L[12] = m2l_fma(-D[65], m, L[12]);
+      L[13] = m2l_fma(-D[68], m, L[13]);
+      L[14] = m2l_fma(-D[69], m, L[14]);
+      L[15] = m2l_fma(-D[70], m, L[15]);
+      L[16] = m2l_fma(-D[73], m, L[16]);
+      L[17] = m2l_fma(-D[74], m, L[17]);
+      L[18] = m2l_fma(-D[75], m, L[18]);
+      L[19] = m2l_fma(-D[76], m, L[19]);
     }
-    { const float m = __ldg(Ms + 16);
-      L[1] = fmaf(-D[26], m, L[1]);
-      L[2] = fmaf(-D[30], m, L[2]);
-      L[3] = fmaf(-D[31], m, L[3]);
-      L[4] = fmaf(D[41], m, L[4]);
-      L[5] = fmaf(D[45], m, L[5]);
-      L[6] = fmaf(D[46], m, L[6]);
-      L[7] = fmaf(D[50], m, L[7]);
-      L[8] = fmaf(D[51], m, L[8]);
-      L[9] = fmaf(D[52], m, L[9]);
-      L[10] = fmaf(-D[62], m, L[10]);
-      L[11] = fmaf(-D[66], m, L[11]);
-      L[12] = fmaf(-D[67], m, L[12]);
-      L[13] = fmaf(-D[71], m, L[13]);
-      L[14] = fmaf(-D[72], m, L[14]);
-      L[15] = fmaf(-D[73], m, L[15]);
-      L[16] = fmaf(-D[77], m, L[16]);
-      L[17] = fmaf(-D[78], m, L[17]);
-      L[18] = fmaf(-D[79], m, L[18]);
-      L[19] = fmaf(-D[80], m, L[19]);
+    { const T m = __ldg(Ms + 16);
+      L[1] = m2l_fma(-D[26], m, L[1]);
+      L[2] = m2l_fma(-D[30], m, L[2]);
+      L[3] = m2l_fma(-D[31], m, L[3]);
+      L[4] = m2l_fma(D[41], m, L[4]);
+      L[5] = m2l_fma(D[45], m, L[5]);
+      L[6] = m2l_fma(D[46], m, L[6]);
+      L[7] = m2l_fma(D[50], m, L[7]);
+      L[8] = m2l_fma(D[51], m, L[8]);
+      L[9] = m2l_fma(D[52], m, L[9]);
+      L[10] = m2l_fma(-D[62], m, L[10]);
+      L[11] = m2l_fma(-D[66], m, L[11]);
+      L[12] = m2l_fma(-D[67], m, L[12]);
+      L[13] = m2l_fma(-D[71], m, L[13]);
+      L[14] = m2l_fma(-D[72], m, L[14]);
+      L[15] = m2l_fma(-D[73], m, L[15]);
+      L[16] = m2l_fma(-D[77], m, L[16]);
+      L[17] = m2l_fma(-D[78], m, L[17]);
+      L[18] = m2l_fma(-D[79], m, L[18]);
+      L[19] = m2l_fma(-D[80], m, L[19]);
     }
-    { const float m = __ldg(Ms + 17);
-      L[1] = fmaf(-D[27], m, L[1]);
-      L[2] = fmaf(-D[31], m, L[2]);
-      L[3] = fmaf(-D[32], m, L[3]);
-      L[4] = fmaf(D[42], m, L[4]);
-      L[5] = fmaf(D[46], m, L[5]);
-      L[6] = fmaf(D[47], m, L[6]);
-      L[7] = fmaf(D[51], m, L[7]);
-      L[8] = fmaf(D[52], m, L[8]);
-      L[9] = fmaf(D[53], m, L[9]);
-      L[10] = fmaf(-D[63], m, L[10]);
-      L[11] = fmaf(-D[67], m, L[11]);
-      L[12] = fmaf(-D[68], m, L[12]);
-      L[13] = fmaf(-D[72], m, L[13]);
-      L[14] = fmaf(-D[73], m, L[14]);
-      L[15] = fmaf(-D[74], m, L[15]);
-      L[16] = fmaf(-D[78], m, L[16]);
-      L[17] = fmaf(-D[79], m, L[17]);
-      L[18] = fmaf(-D[80], m, L[18]);
-      L[19] = fmaf(-D[81], m, L[19]);
+    { const T m = __ldg(Ms + 17);
+      L[1] = m2l_fma(-D[27], m, L[1]);
+      L[2] = m2l_fma(-D[31], m, L[2]);
+      L[3] = m2l_fma(-D[32], m, L[3]);
+      L[4] = m2l_fma(D[42], m, L[4]);
+      L[5] = m2l_fma(D[46], m, L[5]);
+      L[6] = m2l_fma(D[47], m, L[6]);
+      L[7] = m2l_fma(D[51], m, L[7]);
+      L[8] = m2l_fma(D[52], m, L[8]);
+      L[9] = m2l_fma(D[53], m, L[9]);
+      L[10] = m2l_fma(-D[63], m, L[10]);
+      L[11] = m2l_fma(-D[67], m, L[11]);
+      L[12] = m2l_fma(-D[68], m, L[12]);
+      L[13] = m2l_fma(-D[72], m, L[13]);
+      L[14] = m2l_fma(-D[73], m, L[14]);
+      L[15] = m2l_fma(-D[74], m, L[15]);
+      L[16] = m2l_fma(-D[78], m, L[16]);
+      L[17] = m2l_fma(-D[79], m, L[17]);
+      L[18] = m2l_fma(-D[80], m, L[18]);
+      L[19] = m2l_fma(-D[81], m, L[19]);
     }
-    { const float m = __ldg(Ms + 18);
-      L[1] = fmaf(-D[28], m, L[1]);
-      L[2] = fmaf(-D[32], m, L[2]);
-      L[3] = fmaf(-D[33], m, L[3]);
-      L[4] = fmaf(D[43], m, L[4]);
-      L[5] = fmaf(D[47], m, L[5]);
-      L[6] = fmaf(D[48], m, L[6]);
-      L[7] = fmaf(D[52], m, L[7]);
-      L[8] = fmaf(D[53], m, L[8]);
-      L[9] = fmaf(D[54], m, L[9]);
-      L[10] = fmaf(-D[64], m, L[10]);
-      L[11] = fmaf(-D[68], m, L[11]);
-      L[12] = fmaf(-D[69], m, L[12]);
-      L[13] = fmaf(-D[73], m, L[13]);
-      L[14] = fmaf(-D[74], m, L[14]);
-      L[15] = fmaf(-D[75], m, L[15]);
-      L[16] = fmaf(-D[79], m, L[16]);
-      L[17] = fmaf(-D[80], m, L[17]);
-      L[18] = fmaf(-D[81], m, L[18]);
-      L[19] = fmaf(-D[82], m, L[19]);
+    { const T m = __ldg(Ms + 18);
+      L[1] = m2l_fma(-D[28], m, L[1]);
+      L[2] = m2l_fma(-D[32], m, L[2]);
+      L[3] = m2l_fma(-D[33], m, L[3]);
+      L[4] = m2l_fma(D[43], m, L[4]);
+      L[5] = m2l_fma(D[47], m, L[5]);
+      L[6] = m2l_fma(D[48], m, L[6]);
+      L[7] = m2l_fma(D[52], m, L[7]);
+      L[8] = m2l_fma(D[53], m, L[8]);
+      L[9] = m2l_fma(D[54], m, L[9]);
+      L[10] = m2l_fma(-D[64], m, L[10]);
+      L[11] = m2l_fma(-D[68], m, L[11]);
+      L[12] = m2l_fma(-D[69], m, L[12]);
+      L[13] = m2l_fma(-D[73], m, L[13]);
+      L[14] = m2l_fma(-D[74], m, L[14]);
+      L[15] = m2l_fma(-D[75], m, L[15]);
+      L[16] = m2l_fma(-D[79], m, L[16]);
+      L[17] = m2l_fma(-D[80], m, L[17]);
+      L[18] = m2l_fma(-D[81], m, L[18]);
+      L[19] = m2l_fma(-D[82], m, L[19]);
     }
-    { const float m = __ldg(Ms + 19);
-      L[1] = fmaf(-D[29], m, L[1]);
-      L[2] = fmaf(-D[33], m, L[2]);
-      L[3] = fmaf(-D[34], m, L[3]);
-      L[4] = fmaf(D[44], m, L[4]);
-      L[5] = fmaf(D[48], m, L[5]);
-      L[6] = fmaf(D[49], m, L[6]);
-      L[7] = fmaf(D[53], m, L[7]);
-      L[8] = fmaf(D[54], m, L[8]);
-      L[9] = fmaf(D[55], m, L[9]);
-      L[10] = fmaf(-D[65], m, L[10]);
-      L[11] = fmaf(-D[69], m, L[11]);
-      L[12] = fmaf(-D[70], m, L[12]);
-      L[13] = fmaf(-D[74], m, L[13]);
-      L[14] = fmaf(-D[75], m, L[14]);
-      L[15] = fmaf(-D[76], m, L[15]);
-      L[16] = fmaf(-D[80], m, L[16]);
-      L[17] = fmaf(-D[81], m, L[17]);
-      L[18] = fmaf(-D[82], m, L[18]);
-      L[19] = fmaf(-D[83], m, L[19]);
+    { const T m = __ldg(Ms + 19);
+      L[1] = m2l_fma(-D[29], m, L[1]);
+      L[2] = m2l_fma(-D[33], m, L[2]);
+      L[3] = m2l_fma(-D[34], m, L[3]);
+      L[4] = m2l_fma(D[44], m, L[4]);
+      L[5] = m2l_fma(D[48], m, L[5]);
+      L[6] = m2l_fma(D[49], m, L[6]);
+      L[7] = m2l_fma(D[53], m, L[7]);
+      L[8] = m2l_fma(D[54], m, L[8]);
+      L[9] = m2l_fma(D[55], m, L[9]);
+      L[10] = m2l_fma(-D[65], m, L[10]);
+      L[11] = m2l_fma(-D[69], m, L[11]);
+      L[12] = m2l_fma(-D[70], m, L[12]);
+      L[13] = m2l_fma(-D[74], m, L[13]);
+      L[14] = m2l_fma(-D[75], m, L[14]);
+      L[15] = m2l_fma(-D[76], m, L[15]);
+      L[16] = m2l_fma(-D[80], m, L[16]);
+      L[17] = m2l_fma(-D[81], m, L[17]);
+      L[18] = m2l_fma(-D[82], m, L[18]);
+      L[19] = m2l_fma(-D[83], m, L[19]);
     }
-    { const float m = __ldg(Ms + 20);
-      L[1] = fmaf(-D[35], m, L[1]);
-      L[2] = fmaf(-D[36], m, L[2]);
-      L[3] = fmaf(-D[37], m, L[3]);
-      L[4] = fmaf(D[56], m, L[4]);
-      L[5] = fmaf(D[57], m, L[5]);
-      L[6] = fmaf(D[58], m, L[6]);
-      L[7] = fmaf(D[59], m, L[7]);
-      L[8] = fmaf(D[60], m, L[8]);
-      L[9] = fmaf(D[61], m, L[9]);
+    { const T m = __ldg(Ms + 20);
+      L[1] = m2l_fma(-D[35], m, L[1]);
+      L[2] = m2l_fma(-D[36], m, L[2]);
+      L[3] = m2l_fma(-D[37], m, L[3]);
+      L[4] = m2l_fma(D[56], m, L[4]);
+      L[5] = m2l_fma(D[57], m, L[5]);
+      L[6] = m2l_fma(D[58], m, L[6]);
+      L[7] = m2l_fma(D[59], m, L[7]);
+      L[8] = m2l_fma(D[60], m, L[8]);
+      L[9] = m2l_fma(D[61], m, L[9]);
     }
-    { const float m = __ldg(Ms + 21);
-      L[1] = fmaf(-D[36], m, L[1]);
-      L[2] = fmaf(-D[38], m, L[2]);
-      L[3] = fmaf(-D[39], m, L[3]);
-      L[4] = fmaf(D[57], m, L[4]);
-      L[5] = fmaf(D[59], m, L[5]);
-      L[6] = fmaf(D[60], m, L[6]);
-      L[7] = fmaf(D[62], m, L[7]);
-      L[8] = fmaf(D[63], m, L[8]);
-      L[9] = fmaf(D[64], m, L[9]);
+    { const T m = __ldg(Ms + 21);
+      L[1] = m2l_fma(-D[36], m, L[1]);
+      L[2] = m2l_fma(-D[38], m, L[2]);
+      L[3] = m2l_fma(-D[39], m, L[3]);
+      L[4] = m2l_fma(D[57], m, L[4]);
+      L[5] = m2l_fma(D[59], m, L[5]);
+      L[6] = m2l_fma(D[60], m, L[6]);
+      L[7] = m2l_fma(D[62], m, L[7]);
+      L[8] = m2l_fma(D[63], m, L[8]);
+      L[9] = m2l_fma(D[64], m, L[9]);
     }
-    { const float m = __ldg(Ms + 22);
-      L[1] = fmaf(-D[37], m, L[1]);
-      L[2] = fmaf(-D[39], m, L[2]);
-      L[3] = fmaf(-D[40], m, L[3]);
-      L[4] = fmaf(D[58], m, L[4]);
-      L[5] = fmaf(D[60], m, L[5]);
-      L[6] = fmaf(D[61], m, L[6]);
-      L[7] = fmaf(D[63], m, L[7]);
-      L[8] = fmaf(D[64], m, L[8]);
-      L[9] = fmaf(D[65], m, L[9]);
+    { const T m = __ldg(Ms + 22);
+      L[1] = m2l_fma(-D[37], m, L[1]);
+      L[2] = m2l_fma(-D[39], m, L[2]);
+      L[3] = m2l_fma(-D[40], m, L[3]);
+      L[4] = m2l_fma(D[58], m, L[4]);
+      L[5] = m2l_fma(D[60], m, L[5]);
+      L[6] = m2l_fma(D[61], m, L[6]);
+      L[7] = m2l_fma(D[63], m, L[7]);
+      L[8] = m2l_fma(D[64], m, L[8]);
+      L[9] = m2l_fma(D[65], m, L[9]);
     }
-    { const float m = __ldg(Ms + 23);
-      L[1] = fmaf(-D[38], m, L[1]);
-      L[2] = fmaf(-D[41], m, L[2]);
-      L[3] = fmaf(-D[42], m, L[3]);
-      L[4] = fmaf(D[59], m, L[4]);
-      L[5] = fmaf(D[62], m, L[5]);
-      L[6] = fmaf(D[63], m, L[6]);
-      L[7] = fmaf(D[66], m, L[7]);
-      L[8] = fmaf(D[67], m, L[8]);
-      L[9] = fmaf(D[68], m, L[9]);
+    { const T m = __ldg(Ms + 23);
+      L[1] = m2l_fma(-D[38], m, L[1]);
+      L[2] = m2l_fma(-D[41], m, L[2]);
+      L[3] = m2l_fma(-D[42], m, L[3]);
+      L[4] = m2l_fma(D[59], m, L[4]);
+      L[5] = m2l_fma(D[62], m, L[5]);
+      L[6] = m2l_fma(D[63], m, L[6]);
+      L[7] = m2l_fma(D[66], m, L[7]);
+      L[8] = m2l_fma(D[67], m, L[8]);
+      L[9] = m2l_fma(D[68], m, L[9]);
     }
-    { const float m = __ldg(Ms + 24);
-      L[1] = fmaf(-D[39], m, L[1]);
-      L[2] = fmaf(-D[42], m, L[2]);
-      L[3] = fmaf(-D[43], m, L[3]);
-      L[4] = fmaf(D[60], m, L[4]);
-      L[5] = fmaf(D[63], m, L[5]);
-      L[6] = fmaf(D[64], m, L[6]);
-      L[7] = fmaf(D[67], m, L[7]);
-      L[8] = fmaf(D[68], m, L[8]);
-      L[9] = fmaf(D[69], m, L[9]);
+    { const T m = __ldg(Ms + 24);
+      L[1] = m2l_fma(-D[39], m, L[1]);
+      L[2] = m2l_fma(-D[42], m, L[2]);
+      L[3] = m2l_fma(-D[43], m, L[3]);
+      L[4] = m2l_fma(D[60], m, L[4]);
+      L[5] = m2l_fma(D[63], m, L[5]);
+      L[6] = m2l_fma(D[64], m, L[6]);
+      L[7] = m2l_fma(D[67], m, L[7]);
+      L[8] = m2l_fma(D[68], m, L[8]);
+      L[9] = m2l_fma(D[69], m, L[9]);
     }
-    { const float m = __ldg(Ms + 25);
-      L[1] = fmaf(-D[40], m, L[1]);
-      L[2] = fmaf(-D[43], m, L[2]);
-      L[3] = fmaf(-D[44], m, L[3]);
-      L[4] = fmaf(D[61], m, L[4]);
-      L[5] = fmaf(D[64], m, L[5]);
-      L[6] = fmaf(D[65], m, L[6]);
-      L[7] = fmaf(D[68], m, L[7]);
-      L[8] = fmaf(D[69], m, L[8]);
-      L[9] = fmaf(D[70], m, L[9]);
+    { const T m = __ldg(Ms + 25);
+      L[1] = m2l_fma(-D[40], m, L[1]);
+      L[2] = m2l_fma(-D[43], m, L[2]);
+      L[3] = m2l_fma(-D[44], m, L[3]);
+      L[4] = m2l_fma(D[61], m, L[4]);
+      L[5] = m2l_fma(D[64], m, L[5]);
+      L[6] = m2l_fma(D[65], m, L[6]);
+      L[7] = m2l_fma(D[68], m, L[7]);
+      L[8] = m2l_fma(D[69], m, L[8]);
+      L[9] = m2l_fma(D[70], m, L[9]);
     }
-    { const float m = __ldg(Ms + 26);
-      L[1] = fmaf(-D[41], m, L[1]);
-      L[2] = fmaf(-D[45], m, L[2]);
-      L[3] = fmaf(-D[46], m, L[3]);
-      L[4] = fmaf(D[62], m, L[4]);
-      L[5] = fmaf(D[66], m, L[5]);
-      L[6] = fmaf(D[67], m, L[6]);
-      L[7] = fmaf(D[71], m, L[7]);
-      L[8] = fmaf(D[72], m, L[8]);
-      L[9] = fmaf(D[73], m, L[9]);
+    { const T m = __ldg(Ms + 26);
+      L[1] = m2l_fma(-D[41], m, L[1]);
+      L[2] = m2l_fma(-D[45], m, L[2]);
+      L[3] = m2l_fma(-D[46], m, L[3]);
+      L[4] = m2l_fma(D[62], m, L[4]);
+      L[5] = m2l_fma(D[66], m, L[5]);
+      L[6] = m2l_fma(D[67], m, L[6]);
+      L[7] = m2l_fma(D[71], m, L[7]);
+      L[8] = m2l_fma(D[72], m, L[8]);
+      L[9] = m2l_fma(D[73], m, L[9]);
     }
-    { const float m = __ldg(Ms + 27);
-      L[1] = fmaf(-D[42], m, L[1]);
-      L[2] = fmaf(-D[46], m, L[2]);
-      L[3] = fmaf(-D[47], m, L[3]);
-      L[4] = fmaf(D[63], m, L[4]);
-      L[5] = fmaf(D[67], m, L[5]);
-      L[6] = fmaf(D[68], m, L[6]);
-      L[7] = fmaf(D[72], m, L[7]);
-      L[8] = fmaf(D[73], m, L[8]);
-      L[9] = fmaf(D[74], m, L[9]);
+    { const T m = __ldg(Ms + 27);
+      L[1] = m2l_fma(-D[42], m, L[1]);
+      L[2] = m2l_fma(-D[46], m, L[2]);
+      L[3] = m2l_fma(-D[47], m, L[3]);
+      L[4] = m2l_fma(D[63], m, L[4]);
+      L[5] = m2l_fma(D[67], m, L[5]);
+      L[6] = m2l_fma(D[68], m, L[6]);
+      L[7] = m2l_fma(D[72], m, L[7]);
+      L[8] = m2l_fma(D[73], m, L[8]);
+      L[9] = m2l_fma(D[74], m, L[9]);
     }
-    { const float m = __ldg(Ms + 28);
-      L[1] = fmaf(-D[43], m, L[1]);
-      L[2] = fmaf(-D[47], m, L[2]);
-      L[3] = fmaf(-D[48], m, L[3]);
-      L[4] = fmaf(D[64], m, L[4]);
-      L[5] = fmaf(D[68], m, L[5]);
-      L[6] = fmaf(D[69], m, L[6]);
-      L[7] = fmaf(D[73], m, L[7]);
-      L[8] = fmaf(D[74], m, L[8]);
-      L[9] = fmaf(D[75], m, L[9]);
+    { const T m = __ldg(Ms + 28);
+      L[1] = m2l_fma(-D[43], m, L[1]);
+      L[2] = m2l_fma(-D[47], m, L[2]);
+      L[3] = m2l_fma(-D[48], m, L[3]);
+      L[4] = m2l_fma(D[64], m, L[4]);
+      L[5] = m2l_fma(D[68], m, L[5]);
+      L[6] = m2l_fma(D[69], m, L[6]);
+      L[7] = m2l_fma(D[73], m, L[7]);
+      L[8] = m2l_fma(D[74], m, L[8]);
+      L[9] = m2l_fma(D[75], m, L[9]);
     }
-    { const float m = __ldg(Ms + 29);
-      L[1] = fmaf(-D[44], m, L[1]);
-      L[2] = fmaf(-D[48], m, L[2]);
-      L[3] = fmaf(-D[49], m, L[3]);
-      L[4] = fmaf(D[65], m, L[4]);
-      L[5] = fmaf(D[69], m, L[5]);
-      L[6] = fmaf(D[70], m, L[6]);
-      L[7] = fmaf(D[74], m, L[7]);
-      L[8] = fmaf(D[75], m, L[8]);
-      L[9] = fmaf(D[76], m, L[9]);
+    { const T m = __ldg(Ms + 29);
+      L[1] = m2l_fma(-D[44], m, L[1]);
+      L[2] = m2l_fma(-D[48], m, L[2]);
+      L[3] = m2l_fma(-D[49], m, L[3]);
+      L[4] = m2l_fma(D[65], m, L[4]);
+      L[5] = m2l_fma(D[69], m, L[5]);
+      L[6] = m2l_fma(D[70], m, L[6]);
+      L[7] = m2l_fma(D[74], m, L[7]);
+      L[8] = m2l_fma(D[75], m, L[8]);
+      L[9] = m2l_fma(D[76], m, L[9]);
     }
-    { const float m = __ldg(Ms + 30);
-      L[1] = fmaf(-D[45], m, L[1]);
-      L[2] = fmaf(-D[50], m, L[2]);
-      L[3] = fmaf(-D[51], m, L[3]);
-      L[4] = fmaf(D[66], m, L[4]);
-      L[5] = fmaf(D[71], m, L[5]);
-      L[6] = fmaf(D[72], m, L[6]);
-      L[7] = fmaf(D[77], m, L[7]);
-      L[8] = fmaf(D[78], m, L[8]);
-      L[9] = fmaf(D[79], m, L[9]);
+    { const T m = __ldg(Ms + 30);
+      L[1] = m2l_fma(-D[45], m, L[1]);
+      L[2] = m2l_fma(-D[50], m, L[2]);
+      L[3] = m2l_fma(-D[51], m, L[3]);
+      L[4] = m2l_fma(D[66], m, L[4]);
+      L[5] = m2l_fma(D[71], m, L[5]);
+      L[6] = m2l_fma(D[72], m, L[6]);
+      L[7] = m2l_fma(D[77], m, L[7]);
+      L[8] = m2l_fma(D[78], m, L[8]);
+      L[9] = m2l_fma(D[79], m, L[9]);
     }
-    { const float m = __ldg(Ms + 31);
-      L[1] = fmaf(-D[46], m, L[1]);
-      L[2] = fmaf(-D[51], m, L[2]);
-      L[3] = fmaf(-D[52], m, L[3]);
-      L[4] = fmaf(D[67], m, L[4]);
-      L[5] = fmaf(D[72], m, L[5]);
-      L[6] = fmaf(D[73], m, L[6]);
-      L[7] = fmaf(D[78], m, L[7]);
-      L[8] = fmaf(D[79], m, L[8]);
-      L[9] = fmaf(D[80], m, L[9]);
+    { const T m = __ldg(Ms + 31);
+      L[1] = m2l_fma(-D[46], m, L[1]);
+      L[2] = m2l_fma(-D[51], m, L[2]);
+      L[3] = m2l_fma(-D[52], m, L[3]);
+      L[4] = m2l_fma(D[67], m, L[4]);
+      L[5] = m2l_fma(D[72], m, L[5]);
+      L[6] = m2l_fma(D[73], m, L[6]);
+      L[7] = m2l_fma(D[78], m, L[7]);
+      L[8] = m2l_fma(D[79], m, L[8]);
+      L[9] = m2l_fma(D[80], m, L[9]);
     }
-    { const float m = __ldg(Ms + 32);
-      L[1] = fmaf(-D[47], m, L[1]);
-      L[2] = fmaf(-D[52], m, L[2]);
-      L[3] = fmaf(-D[53], m, L[3]);
-      L[4] = fmaf(D[68], m, L[4]);
-      L[5] = fmaf(D[73], m, L[5]);
-      L[6] = fmaf(D[74], m, L[6]);
-      L[7] = fmaf(D[79], m, L[7]);
-      L[8] = fmaf(D[80], m, L[8]);
-      L[9] = fmaf(D[81], m, L[9]);
+    { const T m = __ldg(Ms + 32);
+      L[1] = m2l_fma(-D[47], m, L[1]);
+      L[2] = m2l_fma(-D[52], m, L[2]);
+      L[3] = m2l_fma(-D[53], m, L[3]);
+      L[4] = m2l_fma(D[68], m, L[4]);
+      L[5] = m2l_fma(D[73], m, L[5]);
+      L[6] = m2l_fma(D[74], m, L[6]);
+      L[7] = m2l_fma(D[79], m, L[7]);
+      L[8] = m2l_fma(D[80], m, L[8]);
+      L[9] = m2l_fma(D[81], m, L[9]);
     }
-    { const float m = __ldg(Ms + 33);
-      L[1] = fmaf(-D[48], m, L[1]);
-      L[2] = fmaf(-D[53], m, L[2]);
-      L[3] = fmaf(-D[54], m, L[3]);
-      L[4] = fmaf(D[69], m, L[4]);
-      L[5] = fmaf(D[74], m, L[5]);
-      L[6] = fmaf(D[75], m, L[6]);
-      L[7] = fmaf(D[80], m, L[7]);
-      L[8] = fmaf(D[81], m, L[8]);
-      L[9] = fmaf(D[82], m, L[9]);
+    { const T m = __ldg(Ms + 33);
+      L[1] = m2l_fma(-D[48], m, L[1]);
+      L[2] = m2l_fma(-D[53], m, L[2]);
+      L[3] = m2l_fma(-D[54], m, L[3]);
+      L[4] = m2l_fma(D[69], m, L[4]);
+      L[5] = m2l_fma(D[74], m, L[5]);
+      L[6] = m2l_fma(D[75], m, L[6]);
+      L[7] = m2l_fma(D[80], m, L[7]);
+      L[8] = m2l_fma(D[81], m, L[8]);
+      L[9] = m2l_fma(D[82], m, L[9]);
     }
-    { const float m = __ldg(Ms + 34);
-      L[1] = fmaf(-D[49], m, L[1]);
-      L[2] = fmaf(-D[54], m, L[2]);
-      L[3] = fmaf(-D[55], m, L[3]);
-      L[4] = fmaf(D[70], m, L[4]);
-      L[5] = fmaf(D[75], m, L[5]);
-      L[6] = fmaf(D[76], m, L[6]);
-      L[7] = fmaf(D[81], m, L[7]);
-      L[8] = fmaf(D[82], m, L[8]);
-      L[9] = fmaf(D[83], m, L[9]);
+    { const T m = __ldg(Ms + 34);
+      L[1] = m2l_fma(-D[49], m, L[1]);
+      L[2] = m2l_fma(-D[54], m, L[2]);
+      L[3] = m2l_fma(-D[55], m, L[3]);
+      L[4] = m2l_fma(D[70], m, L[4]);
+      L[5] = m2l_fma(D[75], m, L[5]);
+      L[6] = m2l_fma(D[76], m, L[6]);
+      L[7] = m2l_fma(D[81], m, L[7]);
+      L[8] = m2l_fma(D[82], m, L[8]);
+      L[9] = m2l_fma(D[83], m, L[9]);
     }
-    { const float m = __ldg(Ms + 35);
-      L[1] = fmaf(-D[56], m, L[1]);
-      L[2] = fmaf(-D[57], m, L[2]);
-      L[3] = fmaf(-D[58], m, L[3]);
+    { const T m = __ldg(Ms + 35);
+      L[1] = m2l_fma(-D[56], m, L[1]);
+      L[2] = m2l_fma(-D[57], m, L[2]);
+      L[3] = m2l_fma(-D[58], m, L[3]);
     }
-    { const float m = __ldg(Ms + 36);
-      L[1] = fmaf(-D[57], m, L[1]);
-      L[2] = fmaf(-D[59], m, L[2]);
-      L[3] = fmaf(-D[60], m, L[3]);
+    { const T m = __ldg(Ms + 36);
+      L[1] = m2l_fma(-D[57], m, L[1]);
+      L[2] = m2l_fma(-D[59], m, L[2]);
+      L[3] = m2l_fma(-D[60], m, L[3]);
     }
-    { const float m = __ldg(Ms + 37);
-      L[1] = fmaf(-D[58], m, L[1]);
-      L[2] = fmaf(-D[60], m, L[2]);
-      L[3] = fmaf(-D[61], m, L[3]);
+    { const T m = __ldg(Ms + 37);
+      L[1] = m2l_fma(-D[58], m, L[1]);
+      L[2] = m2l_fma(-D[60], m, L[2]);
+      L[3] = m2l_fma(-D[61], m, L[3]);
     }
-    { const float m = __ldg(Ms + 38);
-      L[1] = fmaf(-D[59], m, L[1]);
-      L[2] = fmaf(-D[62], m, L[2]);
-      L[3] = fmaf(-D[63], m, L[3]);
+    { const T m = __ldg(Ms + 38);
+      L[1] = m2l_fma(-D[59], m, L[1]);
+      L[2] = m2l_fma(-D[62], m, L[2]);
+      L[3] = m2l_fma(-D[63], m, L[3]);
     }
-    { const float m = __ldg(Ms + 39);
-      L[1] = fmaf(-D[60], m, L[1]);
-      L[2] = fmaf(-D[63], m, L[2]);
-      L[3] = fmaf(-D[64], m, L[3]);
+    { const T m = __ldg(Ms + 39);
+      L[1] = m2l_fma(-D[60], m, L[1]);
+      L[2] = m2l_fma(-D[63], m, L[2]);
+      L[3] = m2l_fma(-D[64], m, L[3]);
     }
-    { const float m = __ldg(Ms + 40);
-      L[1] = fmaf(-D[61], m, L[1]);
-      L[2] = fmaf(-D[64], m, L[2]);
-      L[3] = fmaf(-D[65], m, L[3]);
+    { const T m = __ldg(Ms + 40);
+      L[1] = m2l_fma(-D[61], m, L[1]);
+      L[2] = m2l_fma(-D[64], m, L[2]);
+      L[3] = m2l_fma(-D[65], m, L[3]);
     }
-    { const float m = __ldg(Ms + 41);
-      L[1] = fmaf(-D[62], m, L[1]);
-      L[2] = fmaf(-D[66], m, L[2]);
-      L[3] = fmaf(-D[67], m, L[3]);
+    { const T m = __ldg(Ms + 41);
+      L[1] = m2l_fma(-D[62], m, L[1]);
+      L[2] = m2l_fma(-D[66], m, L[2]);
+      L[3] = m2l_fma(-D[67], m, L[3]);
     }
-    { const float m = __ldg(Ms + 42);
-      L[1] = fmaf(-D[63], m, L[1]);
-      L[2] = fmaf(-D[67], m, L[2]);
-      L[3] = fmaf(-D[68], m, L[3]);
+    { const T m = __ldg(Ms + 42);
+      L[1] = m2l_fma(-D[63], m, L[1]);
+      L[2] = m2l_fma(-D[67], m, L[2]);
+      L[3] = m2l_fma(-D[68], m, L[3]);
     }
-    { const float m = __ldg(Ms + 43);
-      L[1] = fmaf(-D[64], m, L[1]);
-      L[2] = fmaf(-D[68], m, L[2]);
-      L[3] = fmaf(-D[69], m, L[3]);
+    { const T m = __ldg(Ms + 43);
+      L[1] = m2l_fma(-D[64], m, L[1]);
+      L[2] = m2l_fma(-D[68], m, L[2]);
+      L[3] = m2l_fma(-D[69], m, L[3]);
     }
-    { const float m = __ldg(Ms + 44);
-      L[1] = fmaf(-D[65], m, L[1]);
-      L[2] = fmaf(-D[69], m, L[2]);
-      L[3] = fmaf(-D[70], m, L[3]);
+    { const T m = __ldg(Ms + 44);
+      L[1] = m2l_fma(-D[65], m, L[1]);
+      L[2] = m2l_fma(-D[69], m, L[2]);
+      L[3] = m2l_fma(-D[70], m, L[3]);
     }
-    { const float m = __ldg(Ms + 45);
-      L[1] = fmaf(-D[66], m, L[1]);
-      L[2] = fmaf(-D[71], m, L[2]);
-      L[3] = fmaf(-D[72], m, L[3]);
+    { const T m = __ldg(Ms + 45);
+      L[1] = m2l_fma(-D[66], m, L[1]);
+      L[2] = m2l_fma(-D[71], m, L[2]);
+      L[3] = m2l_fma(-D[72], m, L[3]);
     }
-    { const float m = __ldg(Ms + 46);
-      L[1] = fmaf(-D[67], m, L[1]);
-      L[2] = fmaf(-D[72], m, L[2]);
-      L[3] = fmaf(-D[73], m, L[3]);
+    { const T m = __ldg(Ms + 46);
+      L[1] = m2l_fma(-D[67], m, L[1]);
+      L[2] = m2l_fma(-D[72], m, L[2]);
+      L[3] = m2l_fma(-D[73], m, L[3]);
     }
-    { const float m = __ldg(Ms + 47);
-      L[1] = fmaf(-D[68], m, L[1]);
-      L[2] = fmaf(-D[73], m, L[2]);
-      L[3] = fmaf(-D[74], m, L[3]);
+    { const T m = __ldg(Ms + 47);
+      L[1] = m2l_fma(-D[68], m, L[1]);
+      L[2] = m2l_fma(-D[73], m, L[2]);
+      L[3] = m2l_fma(-D[74], m, L[3]);
     }
-    { const float m = __ldg(Ms + 48);
-      L[1] = fmaf(-D[69], m, L[1]);
-      L[2] = fmaf(-D[74], m, L[2]);
-      L[3] = fmaf(-D[75], m, L[3]);
+    { const T m = __ldg(Ms + 48);
+      L[1] = m2l_fma(-D[69], m, L[1]);
+      L[2] = m2l_fma(-D[74], m, L[2]);
+      L[3] = m2l_fma(-D[75], m, L[3]);
     }
-    { const float m = __ldg(Ms + 49);
-      L[1] = fmaf(-D[70], m, L[1]);
-      L[2] = fmaf(-D[75], m, L[2]);
-      L[3] = fmaf(-D[76], m, L[3]);
+    { const T m = __ldg(Ms + 49);
+      L[1] = m2l_fma(-D[70], m, L[1]);
+      L[2] = m2l_fma(-D[75], m, L[2]);
+      L[3] = m2l_fma(-D[76], m, L[3]);
     }
-    { const float m = __ldg(Ms + 50);
-      L[1] = fmaf(-D[71], m, L[1]);
-      L[2] = fmaf(-D[77], m, L[2]);
-      L[3] = fmaf(-D[78], m, L[3]);
+    { const T m = __ldg(Ms + 50);
+      L[1] = m2l_fma(-D[71], m, L[1]);
+      L[2] = m2l_fma(-D[77], m, L[2]);
+      L[3] = m2l_fma(-D[78], m, L[3]);
     }
-    { const float m = __ldg(Ms + 51);
-      L[1] = fmaf(-D[72], m, L[1]);
-      L[2] = fmaf(-D[78], m, L[2]);
-      L[3] = fmaf(-D[79], m, L[3]);
+    { const T m = __ldg(Ms + 51);
+      L[1] = m2l_fma(-D[72], m, L[1]);
+      L[2] = m2l_fma(-D[78], m, L[2]);
+      L[3] = m2l_fma(-D[79], m, L[3]);
     }
-    { const float m = __ldg(Ms + 52);
-      L[1] = fmaf(-D[73], m, L[1]);
-      L[2] = fmaf(-D[79], m, L[2]);
-      L[3] = fmaf(-D[80], m, L[3]);
+    { const T m = __ldg(Ms + 52);
+      L[1] = m2l_fma(-D[73], m, L[1]);
+      L[2] = m2l_fma(-D[79], m, L[2]);
+      L[3] = m2l_fma(-D[80], m, L[3]);
     }
-    { const float m = __ldg(Ms + 53);
-      L[1] = fmaf(-D[74], m, L[1]);
-      L[2] = fmaf(-D[80], m, L[2]);
-      L[3] = fmaf(-D[81], m, L[3]);
+    { const T m = __ldg(Ms + 53);
+      L[1] = m2l_fma(-D[74], m, L[1]);
+      L[2] = m2l_fma(-D[80], m, L[2]);
+      L[3] = m2l_fma(-D[81], m, L[3]);
     }
-    { const float m = __ldg(Ms + 54);
-      L[1] = fmaf(-D[75], m, L[1]);
-      L[2] = fmaf(-D[81], m, L[2]);
-      L[3] = fmaf(-D[82], m, L[3]);
+    { const T m = __ldg(Ms + 54);
+      L[1] = m2l_fma(-D[75], m, L[1]);
+      L[2] = m2l_fma(-D[81], m, L[2]);
+      L[3] = m2l_fma(-D[82], m, L[3]);
     }
-    { const float m = __ldg(Ms + 55);
-      L[1] = fmaf(-D[76], m, L[1]);
-      L[2] = fmaf(-D[82], m, L[2]);
-      L[3] = fmaf(-D[83], m, L[3]);
+    { const T m = __ldg(Ms + 55);
+      L[1] = m2l_fma(-D[76], m, L[1]);
+      L[2] = m2l_fma(-D[82], m, L[2]);
+      L[3] = m2l_fma(-D[83], m, L[3]);
     }
 }
 
 template <int P> struct M2LGen;
 template <> struct M2LGen<1> {
     static constexpr int NC = 4;
-    static __device__ __forceinline__ void dtensor(float dx, float dy, float dz, float s, float (&D)[4]) { m2l_dtensor_1(dx, dy, dz, s, D); }
-    static __device__ __forceinline__ void side_a(const float (&D)[4], const float *Ms, float rho, float (&L)[4]) { m2l_side_a_1(D, Ms, rho, L); }
-    static __device__ __forceinline__ void side_b(const float (&D)[4], const float *Ms, float (&L)[4]) { m2l_side_b_1(D, Ms, L); }
-    static __device__ __forceinline__ void side_a_forces(const float (&D)[4], const float *Ms, float rho, float (&L)[4]) { m2l_side_a_forces_1(D, Ms, rho, L); }
-    static __device__ __forceinline__ void side_b_forces(const float (&D)[4], const float *Ms, float (&L)[4]) { m2l_side_b_forces_1(D, Ms, L); }
+    template <class T> static __device__ __forceinline__ void dtensor(T dx, T dy, T dz, T s, T (&D)[4]) { m2l_dtensor_1(dx, dy, dz, s, D); }
+    template <class T> static __device__ __forceinline__ void side_a(const T (&D)[4], const T *Ms, T rho, T (&L)[4]) { m2l_side_a_1(D, Ms, rho, L); }
+    template <class T> static __device__ __forceinline__ void side_b(const T (&D)[4], const T *Ms, T (&L)[4]) { m2l_side_b_1(D, Ms, L); }
+    template <class T> static __device__ __forceinline__ void side_a_forces(const T (&D)[4], const T *Ms, T rho, T (&L)[4]) { m2l_side_a_forces_1(D, Ms, rho, L); }
+    template <class T> static __device__ __forceinline__ void side_b_forces(const T (&D)[4], const T *Ms, T (&L)[4]) { m2l_side_b_forces_1(D, Ms, L); }
 };
 template <> struct M2LGen<2> {
     static constexpr int NC = 10;
-    static __device__ __forceinline__ void dtensor(float dx, float dy, float dz, float s, float (&D)[10]) { m2l_dtensor_2(dx, dy, dz, s, D); }
-    static __device__ __forceinline__ void side_a(const float (&D)[10], const float *Ms, float rho, float (&L)[10]) { m2l_side_a_2(D, Ms, rho, L); }
-    static __device__ __forceinline__ void side_b(const float (&D)[10], const float *Ms, float (&L)[10]) { m2l_side_b_2(D, Ms, L); }
-    static __device__ __forceinline__ void side_a_forces(const float (&D)[10], const float *Ms, float rho, float (&L)[10]) { m2l_side_a_forces_2(D, Ms, rho, L); }
-    static __device__ __forceinline__ void side_b_forces(const float (&D)[10], const float *Ms, float (&L)[10]) { m2l_side_b_forces_2(D, Ms, L); }
+    template <class T> static __device__ __forceinline__ void dtensor(T dx, T dy, T dz, T s, T (&D)[10]) { m2l_dtensor_2(dx, dy, dz, s, D); }
+    template <class T> static __device__ __forceinline__ void side_a(const T (&D)[10], const T *Ms, T rho, T (&L)[10]) { m2l_side_a_2(D, Ms, rho, L); }
+    template <class T> static __device__ __forceinline__ void side_b(const T (&D)[10], const T *Ms, T (&L)[10]) { m2l_side_b_2(D, Ms, L); }
+    template <class T> static __device__ __forceinline__ void side_a_forces(const T (&D)[10], const T *Ms, T rho, T (&L)[10]) { m2l_side_a_forces_2(D, Ms, rho, L); }
+    template <class T> static __device__ __forceinline__ void side_b_forces(const T (&D)[10], const T *Ms, T (&L)[10]) { m2l_side_b_forces_2(D, Ms, L); }
 };
 template <> struct M2LGen<3> {
     static constexpr int NC = 20;
-    static __device__ __forceinline__ void dtensor(float dx, float dy, float dz, float s, float (&D)[20]) { m2l_dtensor_3(dx, dy, dz, s, D); }
-    static __device__ __forceinline__ void side_a(const float (&D)[20], const float *Ms, float rho, float (&L)[20]) { m2l_side_a_3(D, Ms, rho, L); }
-    static __device__ __forceinline__ void side_b(const float (&D)[20], const float *Ms, float (&L)[20]) { m2l_side_b_3(D, Ms, L); }
-    static __device__ __forceinline__ void side_a_forces(const float (&D)[20], const float *Ms, float rho, float (&L)[20]) { m2l_side_a_forces_3(D, Ms, rho, L); }
-    static __device__ __forceinline__ void side_b_forces(const float (&D)[20], const float *Ms, float (&L)[20]) { m2l_side_b_forces_3(D, Ms, L); }
+    template <class T> static __device__ __forceinline__ void dtensor(T dx, T dy, T dz, T s, T (&D)[20]) { m2l_dtensor_3(dx, dy, dz, s, D); }
+    template <class T> static __device__ __forceinline__ void side_a(const T (&D)[20], const T *Ms, T rho, T (&L)[20]) { m2l_side_a_3(D, Ms, rho, L); }
+    template <class T> static __device__ __forceinline__ void side_b(const T (&D)[20], const T *Ms, T (&L)[20]) { m2l_side_b_3(D, Ms, L); }
+    template <class T> static __device__ __forceinline__ void side_a_forces(const T (&D)[20], const T *Ms, T rho, T (&L)[20]) { m2l_side_a_forces_3(D, Ms, rho, L); }
+    template <class T> static __device__ __forceinline__ void side_b_forces(const T (&D)[20], const T *Ms, T (&L)[20]) { m2l_side_b_forces_3(D, Ms, L); }
 };
 template <> struct M2LGen<4> {
     static constexpr int NC = 35;
-    static __device__ __forceinline__ void dtensor(float dx, float dy, float dz, float s, float (&D)[35]) { m2l_dtensor_4(dx, dy, dz, s, D); }
-    static __device__ __forceinline__ void side_a(const float (&D)[35], const float *Ms, float rho, float (&L)[35]) { m2l_side_a_4(D, Ms, rho, L); }
-    static __device__ __forceinline__ void side_b(const float (&D)[35], const float *Ms, float (&L)[35]) { m2l_side_b_4(D, Ms, L); }
-    static __device__ __forceinline__ void side_a_forces(const float (&D)[35], const float *Ms, float rho, float (&L)[35]) { m2l_side_a_forces_4(D, Ms, rho, L); }
-    static __device__ __forceinline__ void side_b_forces(const float (&D)[35], const float *Ms, float (&L)[35]) { m2l_side_b_forces_4(D, Ms, L); }
+    template <class T> static __device__ __forceinline__ void dtensor(T dx, T dy, T dz, T s, T (&D)[35]) { m2l_dtensor_4(dx, dy, dz, s, D); }
+    template <class T> static __device__ __forceinline__ void side_a(const T (&D)[35], const T *Ms, T rho, T (&L)[35]) { m2l_side_a_4(D, Ms, rho, L); }
+    template <class T> static __device__ __forceinline__ void side_b(const T (&D)[35], const T *Ms, T (&L)[35]) { m2l_side_b_4(D, Ms, L); }
+    template <class T> static __device__ __forceinline__ void side_a_forces(const T (&D)[35], const T *Ms, T rho, T (&L)[35]) { m2l_side_a_forces_4(D, Ms, rho, L); }
+    template <class T> static __device__ __forceinline__ void side_b_forces(const T (&D)[35], const T *Ms, T (&L)[35]) { m2l_side_b_forces_4(D, Ms, L); }
 };
 template <> struct M2LGen<5> {
     static constexpr int NC = 56;
-    static __device__ __forceinline__ void dtensor(float dx, float dy, float dz, float s, float (&D)[56]) { m2l_dtensor_5(dx, dy, dz, s, D); }
-    static __device__ __forceinline__ void side_a(const float (&D)[56], const float *Ms, float rho, float (&L)[56]) { m2l_side_a_5(D, Ms, rho, L); }
-    static __device__ __forceinline__ void side_b(const float (&D)[56], const float *Ms, float (&L)[56]) { m2l_side_b_5(D, Ms, L); }
-    static __device__ __forceinline__ void side_a_forces(const float (&D)[56], const float *Ms, float rho, float (&L)[56]) { m2l_side_a_forces_5(D, Ms, rho, L); }
-    static __device__ __forceinline__ void side_b_forces(const float (&D)[56], const float *Ms, float (&L)[56]) { m2l_side_b_forces_5(D, Ms, L); }
+    template <class T> static __device__ __forceinline__ void dtensor(T dx, T dy, T dz, T s, T (&D)[56]) { m2l_dtensor_5(dx, dy, dz, s, D); }
+    template <class T> static __device__ __forceinline__ void side_a(const T (&D)[56], const T *Ms, T rho, T (&L)[56]) { m2l_side_a_5(D, Ms, rho, L); }
+    template <class T> static __device__ __forceinline__ void side_b(const T (&D)[56], const T *Ms, T (&L)[56]) { m2l_side_b_5(D, Ms, L); }
+    template <class T> static __device__ __forceinline__ void side_a_forces(const T (&D)[56], const T *Ms, T rho, T (&L)[56]) { m2l_side_a_forces_5(D, Ms, rho, L); }
+    template <class T> static __device__ __forceinline__ void side_b_forces(const T (&D)[56], const T *Ms, T (&L)[56]) { m2l_side_b_forces_5(D, Ms, L); }
 };
 template <> struct M2LGen<6> {
     static constexpr int NC = 84;
-    static __device__ __forceinline__ void dtensor(float dx, float dy, float dz, float s, float (&D)[84]) { m2l_dtensor_6(dx, dy, dz, s, D); }
-    static __device__ __forceinline__ void side_a(const float (&D)[84], const float *Ms, float rho, float (&L)[84]) { m2l_side_a_6(D, Ms, rho, L); }
-    static __device__ __forceinline__ void side_b(const float (&D)[84], const float *Ms, float (&L)[84]) { m2l_side_b_6(D, Ms, L); }
-    static __device__ __forceinline__ void side_a_forces(const float (&D)[84], const float *Ms, float rho, float (&L)[84]) { m2l_side_a_forces_6(D, Ms, rho, L); }
-    static __device__ __forceinline__ void side_b_forces(const float (&D)[84], const float *Ms, float (&L)[84]) { m2l_side_b_forces_6(D, Ms, L); }
+    template <class T> static __device__ __forceinline__ void dtensor(T dx, T dy, T dz, T s, T (&D)[84]) { m2l_dtensor_6(dx, dy, dz, s, D); }
+    template <class T> static __device__ __forceinline__ void side_a(const T (&D)[84], const T *Ms, T rho, T (&L)[84]) { m2l_side_a_6(D, Ms, rho, L); }
+    template <class T> static __device__ __forceinline__ void side_b(const T (&D)[84], const T *Ms, T (&L)[84]) { m2l_side_b_6(D, Ms, L); }
+    template <class T> static __device__ __forceinline__ void side_a_forces(const T (&D)[84], const T *Ms, T rho, T (&L)[84]) { m2l_side_a_forces_6(D, Ms, rho, L); }
+    template <class T> static __device__ __forceinline__ void side_b_forces(const T (&D)[84], const T *Ms, T (&L)[84]) { m2l_side_b_forces_6(D, Ms, L); }
 };
-__device__ __forceinline__ void m2l_dtensor_h_1(float dx, float dy, float dz, float (&D)[4])
+template <class T> __device__ __forceinline__ void m2l_dtensor_h_1(T dx, T dy, T dz, T (&D)[4])
 {
-    const float s2 = fmaf(dx, dx, fmaf(dy, dy, dz * dz));
-    float si = rsqrtf(s2);
-    si = si * fmaf(-0.5f * s2, si * si, 1.5f);   // one Newton step
-    const float si2 = si * si;
-    const float f0 = -si;
-    const float f1 = -1.0f * f0 * si2;
-    const float r_0_0 = f0;
-    const float r_1_0 = f1;
-    const float r_0_1 = dx * r_1_0;
-    const float r_0_2 = dy * r_1_0;
+    const T s2 = m2l_fma(dx, dx, m2l_fma(dy, dy, dz * dz));
+    const T si = m2l_rsqrt(s2);
+    const T si2 = si * si;
+    const T f0 = -si;
+    const T f1 = T(-1) * f0 * si2;
+    const T r_0_0 = f0;
+    const T r_1_0 = f1;
+    const T r_0_1 = dx * r_1_0;
+    const T r_0_2 = dy * r_1_0;
     D[0] = r_0_0;
     D[1] = r_0_1;
     D[2] = r_0_2;
     D[3] = dz * r_1_0;
 }
 
-__device__ __forceinline__ void m2l_side_a_h_1(const float (&D)[4], const float *__restrict__ Mr, float rho, float (&L)[4])
+template <class T> __device__ __forceinline__ void m2l_side_a_h_1(const T (&D)[4], const T *__restrict__ Mr, T rho, T (&L)[4])
 {
-    float rp = 1.0f;
-    { const float m = __ldg(Mr + 0) * rp;
+    T rp = T(1);
+    { const T m = __ldg(Mr + 0) * rp;
       L[0] = D[0] * m;
       L[1] = D[1] * m;
       L[2] = D[2] * m;
       L[3] = D[3] * m;
     }
     rp *= rho;
-    { const float m = -__ldg(Mr + 1) * rp;
-      L[0] = fmaf(D[1], m, L[0]);
+    { const T m = -__ldg(Mr + 1) * rp;
+      L[0] = m2l_fma(D[1], m, L[0]);
     }
-    { const float m = -__ldg(Mr + 2) * rp;
-      L[0] = fmaf(D[2], m, L[0]);
+    { const T m = -__ldg(Mr + 2) * rp;
+      L[0] = m2l_fma(D[2], m, L[0]);
     }
-    { const float m = -__ldg(Mr + 3) * rp;
-      L[0] = fmaf(D[3], m, L[0]);
+    { const T m = -__ldg(Mr + 3) * rp;
+      L[0] = m2l_fma(D[3], m, L[0]);
     }
 }
 
-__device__ __forceinline__ void m2l_acc_h_1(const float (&D)[4], const float *__restrict__ Mr, float rho, float (&L)[4])
+template <class T> __device__ __forceinline__ void m2l_acc_h_1(const T (&D)[4], const T *__restrict__ Mr, T rho, T (&L)[4])
 {
-    float rp = 1.0f;
-    { const float m = __ldg(Mr + 0) * rp;
-      L[0] = fmaf(D[0], m, L[0]);
-      L[1] = fmaf(D[1], m, L[1]);
-      L[2] = fmaf(D[2], m, L[2]);
-      L[3] = fmaf(D[3], m, L[3]);
+    T rp = T(1);
+    { const T m = __ldg(Mr + 0) * rp;
+      L[0] = m2l_fma(D[0], m, L[0]);
+      L[1] = m2l_fma(D[1], m, L[1]);
+      L[2] = m2l_fma(D[2], m, L[2]);
+      L[3] = m2l_fma(D[3], m, L[3]);
     }
     rp *= rho;
-    { const float m = -__ldg(Mr + 1) * rp;
-      L[0] = fmaf(D[1], m, L[0]);
+    { const T m = -__ldg(Mr + 1) * rp;
+      L[0] = m2l_fma(D[1], m, L[0]);
     }
-    { const float m = -__ldg(Mr + 2) * rp;
-      L[0] = fmaf(D[2], m, L[0]);
+    { const T m = -__ldg(Mr + 2) * rp;
+      L[0] = m2l_fma(D[2], m, L[0]);
     }
-    { const float m = -__ldg(Mr + 3) * rp;
-      L[0] = fmaf(D[3], m, L[0]);
+    { const T m = -__ldg(Mr + 3) * rp;
+      L[0] = m2l_fma(D[3], m, L[0]);
     }
 }
 
-__device__ __forceinline__ void m2l_side_b_h_1(const float (&D)[4], const float *__restrict__ Mr, float (&L)[4])
+template <class T> __device__ __forceinline__ void m2l_side_b_h_1(const T (&D)[4], const T *__restrict__ Mr, T (&L)[4])
 {
-    { const float m = __ldg(Mr + 0);
+    { const T m = __ldg(Mr + 0);
       L[0] = D[0] * m;
       L[1] = -D[1] * m;
       L[2] = -D[2] * m;
       L[3] = -D[3] * m;
     }
-    { const float m = __ldg(Mr + 1);
-      L[0] = fmaf(D[1], m, L[0]);
+    { const T m = __ldg(Mr + 1);
+      L[0] = m2l_fma(D[1], m, L[0]);
     }
-    { const float m = __ldg(Mr + 2);
-      L[0] = fmaf(D[2], m, L[0]);
+    { const T m = __ldg(Mr + 2);
+      L[0] = m2l_fma(D[2], m, L[0]);
     }
-    { const float m = __ldg(Mr + 3);
-      L[0] = fmaf(D[3], m, L[0]);
+    { const T m = __ldg(Mr + 3);
+      L[0] = m2l_fma(D[3], m, L[0]);
     }
 }
 
-__device__ __forceinline__ void m2l_side_a_h_forces_1(const float (&D)[4], const float *__restrict__ Mr, float rho, float (&L)[4])
+template <class T> __device__ __forceinline__ void m2l_side_a_h_forces_1(const T (&D)[4], const T *__restrict__ Mr, T rho, T (&L)[4])
 {
-    L[0] = 0.0f;
-    float rp = 1.0f;
-    { const float m = __ldg(Mr + 0) * rp;
+    L[0] = T(0);
+    T rp = T(1);
+    { const T m = __ldg(Mr + 0) * rp;
       L[1] = D[1] * m;
       L[2] = D[2] * m;
       L[3] = D[3] * m;
     }
 }
 
-__device__ __forceinline__ void m2l_acc_h_forces_1(const float (&D)[4], const float *__restrict__ Mr, float rho, float (&L)[4])
+template <class T> __device__ __forceinline__ void m2l_acc_h_forces_1(const T (&D)[4], const T *__restrict__ Mr, T rho, T (&L)[4])
 {
-    float rp = 1.0f;
-    { const float m = __ldg(Mr + 0) * rp;
-      L[1] = fmaf(D[1], m, L[1]);
-      L[2] = fmaf(D[2], m, L[2]);
-      L[3] = fmaf(D[3], m, L[3]);
+    T rp = T(1);
+    { const T m = __ldg(Mr + 0) * rp;
+      L[1] = m2l_fma(D[1], m, L[1]);
+      L[2] = m2l_fma(D[2], m, L[2]);
+      L[3] = m2l_fma(D[3], m, L[3]);
     }
 }
 
-__device__ __forceinline__ void m2l_side_b_h_forces_1(const float (&D)[4], const float *__restrict__ Mr, float (&L)[4])
+template <class T> __device__ __forceinline__ void m2l_side_b_h_forces_1(const T (&D)[4], const T *__restrict__ Mr, T (&L)[4])
 {
-    L[0] = 0.0f;
-    { const float m = __ldg(Mr + 0);
+    L[0] = T(0);
+    { const T m = __ldg(Mr + 0);
       L[1] = -D[1] * m;
       L[2] = -D[2] * m;
       L[3] = -D[3] * m;
     }
 }
 
-__device__ __forceinline__ void m2l_reduce_moments_h_1(const float *__restrict__ Ms, float *__restrict__ Mr)
+template <class T> __device__ __forceinline__ void m2l_reduce_moments_h_1(const T *__restrict__ Ms, T *__restrict__ Mr)
 {
-    float v0 = Ms[0];
-    float v1 = Ms[1];
-    float v2 = Ms[2];
-    float v3 = Ms[3];
+    T v0 = Ms[0];
+    T v1 = Ms[1];
+    T v2 = Ms[2];
+    T v3 = Ms[3];
     Mr[0] = v0;
     Mr[1] = v1;
     Mr[2] = v2;
     Mr[3] = v3;
 }
 
-__device__ __forceinline__ void m2l_complete_locals_h_1(const float *__restrict__ Lr, float *__restrict__ L)
+template <class T> __device__ __forceinline__ void m2l_complete_locals_h_1(const T *__restrict__ Lr, T *__restrict__ L)
 {
-    const float v0 = Lr[0];
+    const T v0 = Lr[0];
     L[0] = v0;
-    const float v1 = Lr[1];
+    const T v1 = Lr[1];
     L[1] = v1;
-    const float v2 = Lr[2];
+    const T v2 = Lr[2];
     L[2] = v2;
-    const float v3 = Lr[3];
+    const T v3 = Lr[3];
     L[3] = v3;
 }
 
-__device__ __forceinline__ void m2l_dtensor_h_2(float dx, float dy, float dz, float (&D)[10])
+template <class T> __device__ __forceinline__ void m2l_dtensor_h_2(T dx, T dy, T dz, T (&D)[10])
 {
-    const float s2 = fmaf(dx, dx, fmaf(dy, dy, dz * dz));
-    float si = rsqrtf(s2);
-    si = si * fmaf(-0.5f * s2, si * si, 1.5f);   // one Newton step
-    const float si2 = si * si;
-    const float f0 = -si;
-    const float f1 = -1.0f * f0 * si2;
-    const float f2 = -3.0f * f1 * si2;
-    const float r_0_0 = f0;
-    const float r_1_0 = f1;
-    const float r_2_0 = f2;
-    const float r_0_1 = dx * r_1_0;
-    const float r_1_1 = dx * r_2_0;
-    const float r_0_2 = dy * r_1_0;
-    const float r_1_2 = dy * r_2_0;
-    const float r_0_4 = fmaf(1.0f, r_1_0, dx * r_1_1);
-    const float r_0_5 = dx * r_1_2;
-    const float r_0_7 = fmaf(1.0f, r_1_0, dy * r_1_2);
+    const T s2 = m2l_fma(dx, dx, m2l_fma(dy, dy, dz * dz));
+    const T si = m2l_rsqrt(s2);
+    const T si2 = si * si;
+    const T f0 = -si;
+    const T f1 = T(-1) * f0 * si2;
+    const T f2 = T(-3) * f1 * si2;
+    const T r_0_0 = f0;
+    const T r_1_0 = f1;
+    const T r_2_0 = f2;
+    const T r_0_1 = dx * r_1_0;
+    const T r_1_1 = dx * r_2_0;
+    const T r_0_2 = dy * r_1_0;
+    const T r_1_2 = dy * r_2_0;
+    const T r_0_4 = m2l_fma(T(1), r_1_0, dx * r_1_1);
+    const T r_0_5 = dx * r_1_2;
+    const T r_0_7 = m2l_fma(T(1), r_1_0, dy * r_1_2);
     D[0] = r_0_0;
     D[1] = r_0_1;
     D[2] = r_0_2;
@@ -8898,10 +8901,10 @@ __device__ __forceinline__ void m2l_dtensor_h_2(float dx, float dy, float dz, fl
     D[9] = -D[4] - D[7];
 }
 
-__device__ __forceinline__ void m2l_side_a_h_2(const float (&D)[10], const float *__restrict__ Mr, float rho, float (&L)[9])
+template <class T> __device__ __forceinline__ void m2l_side_a_h_2(const T (&D)[10], const T *__restrict__ Mr, T rho, T (&L)[9])
 {
-    float rp = 1.0f;
-    { const float m = __ldg(Mr + 0) * rp;
+    T rp = T(1);
+    { const T m = __ldg(Mr + 0) * rp;
       L[0] = D[0] * m;
       L[1] = D[1] * m;
       L[2] = D[2] * m;
@@ -8913,96 +8916,96 @@ __device__ __forceinline__ void m2l_side_a_h_2(const float (&D)[10], const float
       L[8] = D[8] * m;
     }
     rp *= rho;
-    { const float m = -__ldg(Mr + 1) * rp;
-      L[0] = fmaf(D[1], m, L[0]);
-      L[1] = fmaf(D[4], m, L[1]);
-      L[2] = fmaf(D[5], m, L[2]);
-      L[3] = fmaf(D[6], m, L[3]);
+    { const T m = -__ldg(Mr + 1) * rp;
+      L[0] = m2l_fma(D[1], m, L[0]);
+      L[1] = m2l_fma(D[4], m, L[1]);
+      L[2] = m2l_fma(D[5], m, L[2]);
+      L[3] = m2l_fma(D[6], m, L[3]);
     }
-    { const float m = -__ldg(Mr + 2) * rp;
-      L[0] = fmaf(D[2], m, L[0]);
-      L[1] = fmaf(D[5], m, L[1]);
-      L[2] = fmaf(D[7], m, L[2]);
-      L[3] = fmaf(D[8], m, L[3]);
+    { const T m = -__ldg(Mr + 2) * rp;
+      L[0] = m2l_fma(D[2], m, L[0]);
+      L[1] = m2l_fma(D[5], m, L[1]);
+      L[2] = m2l_fma(D[7], m, L[2]);
+      L[3] = m2l_fma(D[8], m, L[3]);
     }
-    { const float m = -__ldg(Mr + 3) * rp;
-      L[0] = fmaf(D[3], m, L[0]);
-      L[1] = fmaf(D[6], m, L[1]);
-      L[2] = fmaf(D[8], m, L[2]);
-      L[3] = fmaf(D[9], m, L[3]);
+    { const T m = -__ldg(Mr + 3) * rp;
+      L[0] = m2l_fma(D[3], m, L[0]);
+      L[1] = m2l_fma(D[6], m, L[1]);
+      L[2] = m2l_fma(D[8], m, L[2]);
+      L[3] = m2l_fma(D[9], m, L[3]);
     }
     rp *= rho;
-    { const float m = __ldg(Mr + 4) * rp;
-      L[0] = fmaf(D[4], m, L[0]);
+    { const T m = __ldg(Mr + 4) * rp;
+      L[0] = m2l_fma(D[4], m, L[0]);
     }
-    { const float m = __ldg(Mr + 5) * rp;
-      L[0] = fmaf(D[5], m, L[0]);
+    { const T m = __ldg(Mr + 5) * rp;
+      L[0] = m2l_fma(D[5], m, L[0]);
     }
-    { const float m = __ldg(Mr + 6) * rp;
-      L[0] = fmaf(D[6], m, L[0]);
+    { const T m = __ldg(Mr + 6) * rp;
+      L[0] = m2l_fma(D[6], m, L[0]);
     }
-    { const float m = __ldg(Mr + 7) * rp;
-      L[0] = fmaf(D[7], m, L[0]);
+    { const T m = __ldg(Mr + 7) * rp;
+      L[0] = m2l_fma(D[7], m, L[0]);
     }
-    { const float m = __ldg(Mr + 8) * rp;
-      L[0] = fmaf(D[8], m, L[0]);
+    { const T m = __ldg(Mr + 8) * rp;
+      L[0] = m2l_fma(D[8], m, L[0]);
     }
 }
 
-__device__ __forceinline__ void m2l_acc_h_2(const float (&D)[10], const float *__restrict__ Mr, float rho, float (&L)[9])
+template <class T> __device__ __forceinline__ void m2l_acc_h_2(const T (&D)[10], const T *__restrict__ Mr, T rho, T (&L)[9])
 {
-    float rp = 1.0f;
-    { const float m = __ldg(Mr + 0) * rp;
-      L[0] = fmaf(D[0], m, L[0]);
-      L[1] = fmaf(D[1], m, L[1]);
-      L[2] = fmaf(D[2], m, L[2]);
-      L[3] = fmaf(D[3], m, L[3]);
-      L[4] = fmaf(D[4], m, L[4]);
-      L[5] = fmaf(D[5], m, L[5]);
-      L[6] = fmaf(D[6], m, L[6]);
-      L[7] = fmaf(D[7], m, L[7]);
-      L[8] = fmaf(D[8], m, L[8]);
+    T rp = T(1);
+    { const T m = __ldg(Mr + 0) * rp;
+      L[0] = m2l_fma(D[0], m, L[0]);
+      L[1] = m2l_fma(D[1], m, L[1]);
+      L[2] = m2l_fma(D[2], m, L[2]);
+      L[3] = m2l_fma(D[3], m, L[3]);
+      L[4] = m2l_fma(D[4], m, L[4]);
+      L[5] = m2l_fma(D[5], m, L[5]);
+      L[6] = m2l_fma(D[6], m, L[6]);
+      L[7] = m2l_fma(D[7], m, L[7]);
+      L[8] = m2l_fma(D[8], m, L[8]);
     }
     rp *= rho;
-    { const float m = -__ldg(Mr + 1) * rp;
-      L[0] = fmaf(D[1], m, L[0]);
-      L[1] = fmaf(D[4], m, L[1]);
-      L[2] = fmaf(D[5], m, L[2]);
-      L[3] = fmaf(D[6], m, L[3]);
+    { const T m = -__ldg(Mr + 1) * rp;
+      L[0] = m2l_fma(D[1], m, L[0]);
+      L[1] = m2l_fma(D[4], m, L[1]);
+      L[2] = m2l_fma(D[5], m, L[2]);
+      L[3] = m2l_fma(D[6], m, L[3]);
     }
-    { const float m = -__ldg(Mr + 2) * rp;
-      L[0] = fmaf(D[2], m, L[0]);
-      L[1] = fmaf(D[5], m, L[1]);
-      L[2] = fmaf(D[7], m, L[2]);
-      L[3] = fmaf(D[8], m, L[3]);
+    { const T m = -__ldg(Mr + 2) * rp;
+      L[0] = m2l_fma(D[2], m, L[0]);
+      L[1] = m2l_fma(D[5], m, L[1]);
+      L[2] = m2l_fma(D[7], m, L[2]);
+      L[3] = m2l_fma(D[8], m, L[3]);
     }
-    { const float m = -__ldg(Mr + 3) * rp;
-      L[0] = fmaf(D[3], m, L[0]);
-      L[1] = fmaf(D[6], m, L[1]);
-      L[2] = fmaf(D[8], m, L[2]);
-      L[3] = fmaf(D[9], m, L[3]);
+    { const T m = -__ldg(Mr + 3) * rp;
+      L[0] = m2l_fma(D[3], m, L[0]);
+      L[1] = m2l_fma(D[6], m, L[1]);
+      L[2] = m2l_fma(D[8], m, L[2]);
+      L[3] = m2l_fma(D[9], m, L[3]);
     }
     rp *= rho;
-    { const float m = __ldg(Mr + 4) * rp;
-      L[0] = fmaf(D[4], m, L[0]);
+    { const T m = __ldg(Mr + 4) * rp;
+      L[0] = m2l_fma(D[4], m, L[0]);
     }
-    { const float m = __ldg(Mr + 5) * rp;
-      L[0] = fmaf(D[5], m, L[0]);
+    { const T m = __ldg(Mr + 5) * rp;
+      L[0] = m2l_fma(D[5], m, L[0]);
     }
-    { const float m = __ldg(Mr + 6) * rp;
-      L[0] = fmaf(D[6], m, L[0]);
+    { const T m = __ldg(Mr + 6) * rp;
+      L[0] = m2l_fma(D[6], m, L[0]);
     }
-    { const float m = __ldg(Mr + 7) * rp;
-      L[0] = fmaf(D[7], m, L[0]);
+    { const T m = __ldg(Mr + 7) * rp;
+      L[0] = m2l_fma(D[7], m, L[0]);
     }
-    { const float m = __ldg(Mr + 8) * rp;
-      L[0] = fmaf(D[8], m, L[0]);
+    { const T m = __ldg(Mr + 8) * rp;
+      L[0] = m2l_fma(D[8], m, L[0]);
     }
 }
 
-__device__ __forceinline__ void m2l_side_b_h_2(const float (&D)[10], const float *__restrict__ Mr, float (&L)[9])
+template <class T> __device__ __forceinline__ void m2l_side_b_h_2(const T (&D)[10], const T *__restrict__ Mr, T (&L)[9])
 {
-    { const float m = __ldg(Mr + 0);
+    { const T m = __ldg(Mr + 0);
       L[0] = D[0] * m;
       L[1] = -D[1] * m;
       L[2] = -D[2] * m;
@@ -9013,46 +9016,46 @@ __device__ __forceinline__ void m2l_side_b_h_2(const float (&D)[10], const float
       L[7] = D[7] * m;
       L[8] = D[8] * m;
     }
-    { const float m = __ldg(Mr + 1);
-      L[0] = fmaf(D[1], m, L[0]);
-      L[1] = fmaf(-D[4], m, L[1]);
-      L[2] = fmaf(-D[5], m, L[2]);
-      L[3] = fmaf(-D[6], m, L[3]);
+    { const T m = __ldg(Mr + 1);
+      L[0] = m2l_fma(D[1], m, L[0]);
+      L[1] = m2l_fma(-D[4], m, L[1]);
+      L[2] = m2l_fma(-D[5], m, L[2]);
+      L[3] = m2l_fma(-D[6], m, L[3]);
     }
-    { const float m = __ldg(Mr + 2);
-      L[0] = fmaf(D[2], m, L[0]);
-      L[1] = fmaf(-D[5], m, L[1]);
-      L[2] = fmaf(-D[7], m, L[2]);
-      L[3] = fmaf(-D[8], m, L[3]);
+    { const T m = __ldg(Mr + 2);
+      L[0] = m2l_fma(D[2], m, L[0]);
+      L[1] = m2l_fma(-D[5], m, L[1]);
+      L[2] = m2l_fma(-D[7], m, L[2]);
+      L[3] = m2l_fma(-D[8], m, L[3]);
     }
-    { const float m = __ldg(Mr + 3);
-      L[0] = fmaf(D[3], m, L[0]);
-      L[1] = fmaf(-D[6], m, L[1]);
-      L[2] = fmaf(-D[8], m, L[2]);
-      L[3] = fmaf(-D[9], m, L[3]);
+    { const T m = __ldg(Mr + 3);
+      L[0] = m2l_fma(D[3], m, L[0]);
+      L[1] = m2l_fma(-D[6], m, L[1]);
+      L[2] = m2l_fma(-D[8], m, L[2]);
+      L[3] = m2l_fma(-D[9], m, L[3]);
     }
-    { const float m = __ldg(Mr + 4);
-      L[0] = fmaf(D[4], m, L[0]);
+    { const T m = __ldg(Mr + 4);
+      L[0] = m2l_fma(D[4], m, L[0]);
     }
-    { const float m = __ldg(Mr + 5);
-      L[0] = fmaf(D[5], m, L[0]);
+    { const T m = __ldg(Mr + 5);
+      L[0] = m2l_fma(D[5], m, L[0]);
     }
-    { const float m = __ldg(Mr + 6);
-      L[0] = fmaf(D[6], m, L[0]);
+    { const T m = __ldg(Mr + 6);
+      L[0] = m2l_fma(D[6], m, L[0]);
     }
-    { const float m = __ldg(Mr + 7);
-      L[0] = fmaf(D[7], m, L[0]);
+    { const T m = __ldg(Mr + 7);
+      L[0] = m2l_fma(D[7], m, L[0]);
     }
-    { const float m = __ldg(Mr + 8);
-      L[0] = fmaf(D[8], m, L[0]);
+    { const T m = __ldg(Mr + 8);
+      L[0] = m2l_fma(D[8], m, L[0]);
     }
 }
 
-__device__ __forceinline__ void m2l_side_a_h_forces_2(const float (&D)[10], const float *__restrict__ Mr, float rho, float (&L)[9])
+template <class T> __device__ __forceinline__ void m2l_side_a_h_forces_2(const T (&D)[10], const T *__restrict__ Mr, T rho, T (&L)[9])
 {
-    L[0] = 0.0f;
-    float rp = 1.0f;
-    { const float m = __ldg(Mr + 0) * rp;
+    L[0] = T(0);
+    T rp = T(1);
+    { const T m = __ldg(Mr + 0) * rp;
       L[1] = D[1] * m;
       L[2] = D[2] * m;
       L[3] = D[3] * m;
@@ -9063,58 +9066,58 @@ __device__ __forceinline__ void m2l_side_a_h_forces_2(const float (&D)[10], cons
       L[8] = D[8] * m;
     }
     rp *= rho;
-    { const float m = -__ldg(Mr + 1) * rp;
-      L[1] = fmaf(D[4], m, L[1]);
-      L[2] = fmaf(D[5], m, L[2]);
-      L[3] = fmaf(D[6], m, L[3]);
+    { const T m = -__ldg(Mr + 1) * rp;
+      L[1] = m2l_fma(D[4], m, L[1]);
+      L[2] = m2l_fma(D[5], m, L[2]);
+      L[3] = m2l_fma(D[6], m, L[3]);
     }
-    { const float m = -__ldg(Mr + 2) * rp;
-      L[1] = fmaf(D[5], m, L[1]);
-      L[2] = fmaf(D[7], m, L[2]);
-      L[3] = fmaf(D[8], m, L[3]);
+    { const T m = -__ldg(Mr + 2) * rp;
+      L[1] = m2l_fma(D[5], m, L[1]);
+      L[2] = m2l_fma(D[7], m, L[2]);
+      L[3] = m2l_fma(D[8], m, L[3]);
     }
-    { const float m = -__ldg(Mr + 3) * rp;
-      L[1] = fmaf(D[6], m, L[1]);
-      L[2] = fmaf(D[8], m, L[2]);
-      L[3] = fmaf(D[9], m, L[3]);
+    { const T m = -__ldg(Mr + 3) * rp;
+      L[1] = m2l_fma(D[6], m, L[1]);
+      L[2] = m2l_fma(D[8], m, L[2]);
+      L[3] = m2l_fma(D[9], m, L[3]);
     }
 }
 
-__device__ __forceinline__ void m2l_acc_h_forces_2(const float (&D)[10], const float *__restrict__ Mr, float rho, float (&L)[9])
+template <class T> __device__ __forceinline__ void m2l_acc_h_forces_2(const T (&D)[10], const T *__restrict__ Mr, T rho, T (&L)[9])
 {
-    float rp = 1.0f;
-    { const float m = __ldg(Mr + 0) * rp;
-      L[1] = fmaf(D[1], m, L[1]);
-      L[2] = fmaf(D[2], m, L[2]);
-      L[3] = fmaf(D[3], m, L[3]);
-      L[4] = fmaf(D[4], m, L[4]);
-      L[5] = fmaf(D[5], m, L[5]);
-      L[6] = fmaf(D[6], m, L[6]);
-      L[7] = fmaf(D[7], m, L[7]);
-      L[8] = fmaf(D[8], m, L[8]);
+    T rp = T(1);
+    { const T m = __ldg(Mr + 0) * rp;
+      L[1] = m2l_fma(D[1], m, L[1]);
+      L[2] = m2l_fma(D[2], m, L[2]);
+      L[3] = m2l_fma(D[3], m, L[3]);
+      L[4] = m2l_fma(D[4], m, L[4]);
+      L[5] = m2l_fma(D[5], m, L[5]);
+      L[6] = m2l_fma(D[6], m, L[6]);
+      L[7] = m2l_fma(D[7], m, L[7]);
+      L[8] = m2l_fma(D[8], m, L[8]);
     }
     rp *= rho;
-    { const float m = -__ldg(Mr + 1) * rp;
-      L[1] = fmaf(D[4], m, L[1]);
-      L[2] = fmaf(D[5], m, L[2]);
-      L[3] = fmaf(D[6], m, L[3]);
+    { const T m = -__ldg(Mr + 1) * rp;
+      L[1] = m2l_fma(D[4], m, L[1]);
+      L[2] = m2l_fma(D[5], m, L[2]);
+      L[3] = m2l_fma(D[6], m, L[3]);
     }
-    { const float m = -__ldg(Mr + 2) * rp;
-      L[1] = fmaf(D[5], m, L[1]);
-      L[2] = fmaf(D[7], m, L[2]);
-      L[3] = fmaf(D[8], m, L[3]);
+    { const T m = -__ldg(Mr + 2) * rp;
+      L[1] = m2l_fma(D[5], m, L[1]);
+      L[2] = m2l_fma(D[7], m, L[2]);
+      L[3] = m2l_fma(D[8], m, L[3]);
     }
-    { const float m = -__ldg(Mr + 3) * rp;
-      L[1] = fmaf(D[6], m, L[1]);
-      L[2] = fmaf(D[8], m, L[2]);
-      L[3] = fmaf(D[9], m, L[3]);
+    { const T m = -__ldg(Mr + 3) * rp;
+      L[1] = m2l_fma(D[6], m, L[1]);
+      L[2] = m2l_fma(D[8], m, L[2]);
+      L[3] = m2l_fma(D[9], m, L[3]);
     }
 }
 
-__device__ __forceinline__ void m2l_side_b_h_forces_2(const float (&D)[10], const float *__restrict__ Mr, float (&L)[9])
+template <class T> __device__ __forceinline__ void m2l_side_b_h_forces_2(const T (&D)[10], const T *__restrict__ Mr, T (&L)[9])
 {
-    L[0] = 0.0f;
-    { const float m = __ldg(Mr + 0);
+    L[0] = T(0);
+    { const T m = __ldg(Mr + 0);
       L[1] = -D[1] * m;
       L[2] = -D[2] * m;
       L[3] = -D[3] * m;
@@ -9124,35 +9127,35 @@ __device__ __forceinline__ void m2l_side_b_h_forces_2(const float (&D)[10], cons
       L[7] = D[7] * m;
       L[8] = D[8] * m;
     }
-    { const float m = __ldg(Mr + 1);
-      L[1] = fmaf(-D[4], m, L[1]);
-      L[2] = fmaf(-D[5], m, L[2]);
-      L[3] = fmaf(-D[6], m, L[3]);
+    { const T m = __ldg(Mr + 1);
+      L[1] = m2l_fma(-D[4], m, L[1]);
+      L[2] = m2l_fma(-D[5], m, L[2]);
+      L[3] = m2l_fma(-D[6], m, L[3]);
     }
-    { const float m = __ldg(Mr + 2);
-      L[1] = fmaf(-D[5], m, L[1]);
-      L[2] = fmaf(-D[7], m, L[2]);
-      L[3] = fmaf(-D[8], m, L[3]);
+    { const T m = __ldg(Mr + 2);
+      L[1] = m2l_fma(-D[5], m, L[1]);
+      L[2] = m2l_fma(-D[7], m, L[2]);
+      L[3] = m2l_fma(-D[8], m, L[3]);
     }
-    { const float m = __ldg(Mr + 3);
-      L[1] = fmaf(-D[6], m, L[1]);
-      L[2] = fmaf(-D[8], m, L[2]);
-      L[3] = fmaf(-D[9], m, L[3]);
+    { const T m = __ldg(Mr + 3);
+      L[1] = m2l_fma(-D[6], m, L[1]);
+      L[2] = m2l_fma(-D[8], m, L[2]);
+      L[3] = m2l_fma(-D[9], m, L[3]);
     }
 }
 
-__device__ __forceinline__ void m2l_reduce_moments_h_2(const float *__restrict__ Ms, float *__restrict__ Mr)
+template <class T> __device__ __forceinline__ void m2l_reduce_moments_h_2(const T *__restrict__ Ms, T *__restrict__ Mr)
 {
-    float v0 = Ms[0];
-    float v1 = Ms[1];
-    float v2 = Ms[2];
-    float v3 = Ms[3];
-    float v4 = Ms[4];
-    float v5 = Ms[5];
-    float v6 = Ms[6];
-    float v7 = Ms[7];
-    float v8 = Ms[8];
-    float v9 = Ms[9];
+    T v0 = Ms[0];
+    T v1 = Ms[1];
+    T v2 = Ms[2];
+    T v3 = Ms[3];
+    T v4 = Ms[4];
+    T v5 = Ms[5];
+    T v6 = Ms[6];
+    T v7 = Ms[7];
+    T v8 = Ms[8];
+    T v9 = Ms[9];
     v4 -= v9;
     v7 -= v9;
     Mr[0] = v0;
@@ -9166,60 +9169,59 @@ __device__ __forceinline__ void m2l_reduce_moments_h_2(const float *__restrict__
     Mr[8] = v8;
 }
 
-__device__ __forceinline__ void m2l_complete_locals_h_2(const float *__restrict__ Lr, float *__restrict__ L)
+template <class T> __device__ __forceinline__ void m2l_complete_locals_h_2(const T *__restrict__ Lr, T *__restrict__ L)
 {
-    const float v0 = Lr[0];
+    const T v0 = Lr[0];
     L[0] = v0;
-    const float v1 = Lr[1];
+    const T v1 = Lr[1];
     L[1] = v1;
-    const float v2 = Lr[2];
+    const T v2 = Lr[2];
     L[2] = v2;
-    const float v3 = Lr[3];
+    const T v3 = Lr[3];
     L[3] = v3;
-    const float v4 = Lr[4];
+    const T v4 = Lr[4];
     L[4] = v4;
-    const float v5 = Lr[5];
+    const T v5 = Lr[5];
     L[5] = v5;
-    const float v6 = Lr[6];
+    const T v6 = Lr[6];
     L[6] = v6;
-    const float v7 = Lr[7];
+    const T v7 = Lr[7];
     L[7] = v7;
-    const float v8 = Lr[8];
+    const T v8 = Lr[8];
     L[8] = v8;
-    const float v9 = -v4 - v7;
+    const T v9 = -v4 - v7;
     L[9] = v9;
 }
 
-__device__ __forceinline__ void m2l_dtensor_h_3(float dx, float dy, float dz, float (&D)[19])
+template <class T> __device__ __forceinline__ void m2l_dtensor_h_3(T dx, T dy, T dz, T (&D)[19])
 {
-    const float s2 = fmaf(dx, dx, fmaf(dy, dy, dz * dz));
-    float si = rsqrtf(s2);
-    si = si * fmaf(-0.5f * s2, si * si, 1.5f);   // one Newton step
-    const float si2 = si * si;
-    const float f0 = -si;
-    const float f1 = -1.0f * f0 * si2;
-    const float f2 = -3.0f * f1 * si2;
-    const float f3 = -5.0f * f2 * si2;
-    const float r_0_0 = f0;
-    const float r_1_0 = f1;
-    const float r_2_0 = f2;
-    const float r_3_0 = f3;
-    const float r_0_1 = dx * r_1_0;
-    const float r_1_1 = dx * r_2_0;
-    const float r_2_1 = dx * r_3_0;
-    const float r_0_2 = dy * r_1_0;
-    const float r_1_2 = dy * r_2_0;
-    const float r_2_2 = dy * r_3_0;
-    const float r_0_4 = fmaf(1.0f, r_1_0, dx * r_1_1);
-    const float r_1_4 = fmaf(1.0f, r_2_0, dx * r_2_1);
-    const float r_0_5 = dx * r_1_2;
-    const float r_1_5 = dx * r_2_2;
-    const float r_0_7 = fmaf(1.0f, r_1_0, dy * r_1_2);
-    const float r_1_7 = fmaf(1.0f, r_2_0, dy * r_2_2);
-    const float r_0_10 = fmaf(2.0f, r_1_1, dx * r_1_4);
-    const float r_0_11 = fmaf(1.0f, r_1_2, dx * r_1_5);
-    const float r_0_13 = dx * r_1_7;
-    const float r_0_16 = fmaf(2.0f, r_1_2, dy * r_1_7);
+    const T s2 = m2l_fma(dx, dx, m2l_fma(dy, dy, dz * dz));
+    const T si = m2l_rsqrt(s2);
+    const T si2 = si * si;
+    const T f0 = -si;
+    const T f1 = T(-1) * f0 * si2;
+    const T f2 = T(-3) * f1 * si2;
+    const T f3 = T(-5) * f2 * si2;
+    const T r_0_0 = f0;
+    const T r_1_0 = f1;
+    const T r_2_0 = f2;
+    const T r_3_0 = f3;
+    const T r_0_1 = dx * r_1_0;
+    const T r_1_1 = dx * r_2_0;
+    const T r_2_1 = dx * r_3_0;
+    const T r_0_2 = dy * r_1_0;
+    const T r_1_2 = dy * r_2_0;
+    const T r_2_2 = dy * r_3_0;
+    const T r_0_4 = m2l_fma(T(1), r_1_0, dx * r_1_1);
+    const T r_1_4 = m2l_fma(T(1), r_2_0, dx * r_2_1);
+    const T r_0_5 = dx * r_1_2;
+    const T r_1_5 = dx * r_2_2;
+    const T r_0_7 = m2l_fma(T(1), r_1_0, dy * r_1_2);
+    const T r_1_7 = m2l_fma(T(1), r_2_0, dy * r_2_2);
+    const T r_0_10 = m2l_fma(T(2), r_1_1, dx * r_1_4);
+    const T r_0_11 = m2l_fma(T(1), r_1_2, dx * r_1_5);
+    const T r_0_13 = dx * r_1_7;
+    const T r_0_16 = m2l_fma(T(2), r_1_2, dy * r_1_7);
     D[0] = r_0_0;
     D[1] = r_0_1;
     D[2] = r_0_2;
@@ -9241,10 +9243,10 @@ __device__ __forceinline__ void m2l_dtensor_h_3(float dx, float dy, float dz, fl
     D[18] = -D[11] - D[16];
 }
 
-__device__ __forceinline__ void m2l_side_a_h_3(const float (&D)[19], const float *__restrict__ Mr, float rho, float (&L)[16])
+template <class T> __device__ __forceinline__ void m2l_side_a_h_3(const T (&D)[19], const T *__restrict__ Mr, T rho, T (&L)[16])
 {
-    float rp = 1.0f;
-    { const float m = __ldg(Mr + 0) * rp;
+    T rp = T(1);
+    { const T m = __ldg(Mr + 0) * rp;
       L[0] = D[0] * m;
       L[1] = D[1] * m;
       L[2] = D[2] * m;
@@ -9263,207 +9265,207 @@ __device__ __forceinline__ void m2l_side_a_h_3(const float (&D)[19], const float
       L[15] = D[17] * m;
     }
     rp *= rho;
-    { const float m = -__ldg(Mr + 1) * rp;
-      L[0] = fmaf(D[1], m, L[0]);
-      L[1] = fmaf(D[4], m, L[1]);
-      L[2] = fmaf(D[5], m, L[2]);
-      L[3] = fmaf(D[6], m, L[3]);
-      L[4] = fmaf(D[10], m, L[4]);
-      L[5] = fmaf(D[11], m, L[5]);
-      L[6] = fmaf(D[12], m, L[6]);
-      L[7] = fmaf(D[13], m, L[7]);
-      L[8] = fmaf(D[14], m, L[8]);
+    { const T m = -__ldg(Mr + 1) * rp;
+      L[0] = m2l_fma(D[1], m, L[0]);
+      L[1] = m2l_fma(D[4], m, L[1]);
+      L[2] = m2l_fma(D[5], m, L[2]);
+      L[3] = m2l_fma(D[6], m, L[3]);
+      L[4] = m2l_fma(D[10], m, L[4]);
+      L[5] = m2l_fma(D[11], m, L[5]);
+      L[6] = m2l_fma(D[12], m, L[6]);
+      L[7] = m2l_fma(D[13], m, L[7]);
+      L[8] = m2l_fma(D[14], m, L[8]);
     }
-    { const float m = -__ldg(Mr + 2) * rp;
-      L[0] = fmaf(D[2], m, L[0]);
-      L[1] = fmaf(D[5], m, L[1]);
-      L[2] = fmaf(D[7], m, L[2]);
-      L[3] = fmaf(D[8], m, L[3]);
-      L[4] = fmaf(D[11], m, L[4]);
-      L[5] = fmaf(D[13], m, L[5]);
-      L[6] = fmaf(D[14], m, L[6]);
-      L[7] = fmaf(D[16], m, L[7]);
-      L[8] = fmaf(D[17], m, L[8]);
+    { const T m = -__ldg(Mr + 2) * rp;
+      L[0] = m2l_fma(D[2], m, L[0]);
+      L[1] = m2l_fma(D[5], m, L[1]);
+      L[2] = m2l_fma(D[7], m, L[2]);
+      L[3] = m2l_fma(D[8], m, L[3]);
+      L[4] = m2l_fma(D[11], m, L[4]);
+      L[5] = m2l_fma(D[13], m, L[5]);
+      L[6] = m2l_fma(D[14], m, L[6]);
+      L[7] = m2l_fma(D[16], m, L[7]);
+      L[8] = m2l_fma(D[17], m, L[8]);
     }
-    { const float m = -__ldg(Mr + 3) * rp;
-      L[0] = fmaf(D[3], m, L[0]);
-      L[1] = fmaf(D[6], m, L[1]);
-      L[2] = fmaf(D[8], m, L[2]);
-      L[3] = fmaf(D[9], m, L[3]);
-      L[4] = fmaf(D[12], m, L[4]);
-      L[5] = fmaf(D[14], m, L[5]);
-      L[6] = fmaf(D[15], m, L[6]);
-      L[7] = fmaf(D[17], m, L[7]);
-      L[8] = fmaf(D[18], m, L[8]);
-    }
-    rp *= rho;
-    { const float m = __ldg(Mr + 4) * rp;
-      L[0] = fmaf(D[4], m, L[0]);
-      L[1] = fmaf(D[10], m, L[1]);
-      L[2] = fmaf(D[11], m, L[2]);
-      L[3] = fmaf(D[12], m, L[3]);
-    }
-    { const float m = __ldg(Mr + 5) * rp;
-      L[0] = fmaf(D[5], m, L[0]);
-      L[1] = fmaf(D[11], m, L[1]);
-      L[2] = fmaf(D[13], m, L[2]);
-      L[3] = fmaf(D[14], m, L[3]);
-    }
-    { const float m = __ldg(Mr + 6) * rp;
-      L[0] = fmaf(D[6], m, L[0]);
-      L[1] = fmaf(D[12], m, L[1]);
-      L[2] = fmaf(D[14], m, L[2]);
-      L[3] = fmaf(D[15], m, L[3]);
-    }
-    { const float m = __ldg(Mr + 7) * rp;
-      L[0] = fmaf(D[7], m, L[0]);
-      L[1] = fmaf(D[13], m, L[1]);
-      L[2] = fmaf(D[16], m, L[2]);
-      L[3] = fmaf(D[17], m, L[3]);
-    }
-    { const float m = __ldg(Mr + 8) * rp;
-      L[0] = fmaf(D[8], m, L[0]);
-      L[1] = fmaf(D[14], m, L[1]);
-      L[2] = fmaf(D[17], m, L[2]);
-      L[3] = fmaf(D[18], m, L[3]);
+    { const T m = -__ldg(Mr + 3) * rp;
+      L[0] = m2l_fma(D[3], m, L[0]);
+      L[1] = m2l_fma(D[6], m, L[1]);
+      L[2] = m2l_fma(D[8], m, L[2]);
+      L[3] = m2l_fma(D[9], m, L[3]);
+      L[4] = m2l_fma(D[12], m, L[4]);
+      L[5] = m2l_fma(D[14], m, L[5]);
+      L[6] = m2l_fma(D[15], m, L[6]);
+      L[7] = m2l_fma(D[17], m, L[7]);
+      L[8] = m2l_fma(D[18], m, L[8]);
     }
     rp *= rho;
-    { const float m = -__ldg(Mr + 9) * rp;
-      L[0] = fmaf(D[10], m, L[0]);
+    { const T m = __ldg(Mr + 4) * rp;
+      L[0] = m2l_fma(D[4], m, L[0]);
+      L[1] = m2l_fma(D[10], m, L[1]);
+      L[2] = m2l_fma(D[11], m, L[2]);
+      L[3] = m2l_fma(D[12], m, L[3]);
     }
-    { const float m = -__ldg(Mr + 10) * rp;
-      L[0] = fmaf(D[11], m, L[0]);
+    { const T m = __ldg(Mr + 5) * rp;
+      L[0] = m2l_fma(D[5], m, L[0]);
+      L[1] = m2l_fma(D[11], m, L[1]);
+      L[2] = m2l_fma(D[13], m, L[2]);
+      L[3] = m2l_fma(D[14], m, L[3]);
     }
-    { const float m = -__ldg(Mr + 11) * rp;
-      L[0] = fmaf(D[12], m, L[0]);
+    { const T m = __ldg(Mr + 6) * rp;
+      L[0] = m2l_fma(D[6], m, L[0]);
+      L[1] = m2l_fma(D[12], m, L[1]);
+      L[2] = m2l_fma(D[14], m, L[2]);
+      L[3] = m2l_fma(D[15], m, L[3]);
     }
-    { const float m = -__ldg(Mr + 12) * rp;
-      L[0] = fmaf(D[13], m, L[0]);
+    { const T m = __ldg(Mr + 7) * rp;
+      L[0] = m2l_fma(D[7], m, L[0]);
+      L[1] = m2l_fma(D[13], m, L[1]);
+      L[2] = m2l_fma(D[16], m, L[2]);
+      L[3] = m2l_fma(D[17], m, L[3]);
     }
-    { const float m = -__ldg(Mr + 13) * rp;
-      L[0] = fmaf(D[14], m, L[0]);
+    { const T m = __ldg(Mr + 8) * rp;
+      L[0] = m2l_fma(D[8], m, L[0]);
+      L[1] = m2l_fma(D[14], m, L[1]);
+      L[2] = m2l_fma(D[17], m, L[2]);
+      L[3] = m2l_fma(D[18], m, L[3]);
     }
-    { const float m = -__ldg(Mr + 14) * rp;
-      L[0] = fmaf(D[16], m, L[0]);
+    rp *= rho;
+    { const T m = -__ldg(Mr + 9) * rp;
+      L[0] = m2l_fma(D[10], m, L[0]);
     }
-    { const float m = -__ldg(Mr + 15) * rp;
-      L[0] = fmaf(D[17], m, L[0]);
+    { const T m = -__ldg(Mr + 10) * rp;
+      L[0] = m2l_fma(D[11], m, L[0]);
+    }
+    { const T m = -__ldg(Mr + 11) * rp;
+      L[0] = m2l_fma(D[12], m, L[0]);
+    }
+    { const T m = -__ldg(Mr + 12) * rp;
+      L[0] = m2l_fma(D[13], m, L[0]);
+    }
+    { const T m = -__ldg(Mr + 13) * rp;
+      L[0] = m2l_fma(D[14], m, L[0]);
+    }
+    { const T m = -__ldg(Mr + 14) * rp;
+      L[0] = m2l_fma(D[16], m, L[0]);
+    }
+    { const T m = -__ldg(Mr + 15) * rp;
+      L[0] = m2l_fma(D[17], m, L[0]);
     }
 }
 
-__device__ __forceinline__ void m2l_acc_h_3(const float (&D)[19], const float *__restrict__ Mr, float rho, float (&L)[16])
+template <class T> __device__ __forceinline__ void m2l_acc_h_3(const T (&D)[19], const T *__restrict__ Mr, T rho, T (&L)[16])
 {
-    float rp = 1.0f;
-    { const float m = __ldg(Mr + 0) * rp;
-      L[0] = fmaf(D[0], m, L[0]);
-      L[1] = fmaf(D[1], m, L[1]);
-      L[2] = fmaf(D[2], m, L[2]);
-      L[3] = fmaf(D[3], m, L[3]);
-      L[4] = fmaf(D[4], m, L[4]);
-      L[5] = fmaf(D[5], m, L[5]);
-      L[6] = fmaf(D[6], m, L[6]);
-      L[7] = fmaf(D[7], m, L[7]);
-      L[8] = fmaf(D[8], m, L[8]);
-      L[9] = fmaf(D[10], m, L[9]);
-      L[10] = fmaf(D[11], m, L[10]);
-      L[11] = fmaf(D[12], m, L[11]);
-      L[12] = fmaf(D[13], m, L[12]);
-      L[13] = fmaf(D[14], m, L[13]);
-      L[14] = fmaf(D[16], m, L[14]);
-      L[15] = fmaf(D[17], m, L[15]);
+    T rp = T(1);
+    { const T m = __ldg(Mr + 0) * rp;
+      L[0] = m2l_fma(D[0], m, L[0]);
+      L[1] = m2l_fma(D[1], m, L[1]);
+      L[2] = m2l_fma(D[2], m, L[2]);
+      L[3] = m2l_fma(D[3], m, L[3]);
+      L[4] = m2l_fma(D[4], m, L[4]);
+      L[5] = m2l_fma(D[5], m, L[5]);
+      L[6] = m2l_fma(D[6], m, L[6]);
+      L[7] = m2l_fma(D[7], m, L[7]);
+      L[8] = m2l_fma(D[8], m, L[8]);
+      L[9] = m2l_fma(D[10], m, L[9]);
+      L[10] = m2l_fma(D[11], m, L[10]);
+      L[11] = m2l_fma(D[12], m, L[11]);
+      L[12] = m2l_fma(D[13], m, L[12]);
+      L[13] = m2l_fma(D[14], m, L[13]);
+      L[14] = m2l_fma(D[16], m, L[14]);
+      L[15] = m2l_fma(D[17], m, L[15]);
     }
     rp *= rho;
-    { const float m = -__ldg(Mr + 1) * rp;
-      L[0] = fmaf(D[1], m, L[0]);
-      L[1] = fmaf(D[4], m, L[1]);
-      L[2] = fmaf(D[5], m, L[2]);
-      L[3] = fmaf(D[6], m, L[3]);
-      L[4] = fmaf(D[10], m, L[4]);
-      L[5] = fmaf(D[11], m, L[5]);
-      L[6] = fmaf(D[12], m, L[6]);
-      L[7] = fmaf(D[13], m, L[7]);
-      L[8] = fmaf(D[14], m, L[8]);
+    { const T m = -__ldg(Mr + 1) * rp;
+      L[0] = m2l_fma(D[1], m, L[0]);
+      L[1] = m2l_fma(D[4], m, L[1]);
+      L[2] = m2l_fma(D[5], m, L[2]);
+      L[3] = m2l_fma(D[6], m, L[3]);
+      L[4] = m2l_fma(D[10], m, L[4]);
+      L[5] = m2l_fma(D[11], m, L[5]);
+      L[6] = m2l_fma(D[12], m, L[6]);
+      L[7] = m2l_fma(D[13], m, L[7]);
+      L[8] = m2l_fma(D[14], m, L[8]);
     }
-    { const float m = -__ldg(Mr + 2) * rp;
-      L[0] = fmaf(D[2], m, L[0]);
-      L[1] = fmaf(D[5], m, L[1]);
-      L[2] = fmaf(D[7], m, L[2]);
-      L[3] = fmaf(D[8], m, L[3]);
-      L[4] = fmaf(D[11], m, L[4]);
-      L[5] = fmaf(D[13], m, L[5]);
-      L[6] = fmaf(D[14], m, L[6]);
-      L[7] = fmaf(D[16], m, L[7]);
-      L[8] = fmaf(D[17], m, L[8]);
+    { const T m = -__ldg(Mr + 2) * rp;
+      L[0] = m2l_fma(D[2], m, L[0]);
+      L[1] = m2l_fma(D[5], m, L[1]);
+      L[2] = m2l_fma(D[7], m, L[2]);
+      L[3] = m2l_fma(D[8], m, L[3]);
+      L[4] = m2l_fma(D[11], m, L[4]);
+      L[5] = m2l_fma(D[13], m, L[5]);
+      L[6] = m2l_fma(D[14], m, L[6]);
+      L[7] = m2l_fma(D[16], m, L[7]);
+      L[8] = m2l_fma(D[17], m, L[8]);
     }
-    { const float m = -__ldg(Mr + 3) * rp;
-      L[0] = fmaf(D[3], m, L[0]);
-      L[1] = fmaf(D[6], m, L[1]);
-      L[2] = fmaf(D[8], m, L[2]);
-      L[3] = fmaf(D[9], m, L[3]);
-      L[4] = fmaf(D[12], m, L[4]);
-      L[5] = fmaf(D[14], m, L[5]);
-      L[6] = fmaf(D[15], m, L[6]);
-      L[7] = fmaf(D[17], m, L[7]);
-      L[8] = fmaf(D[18], m, L[8]);
-    }
-    rp *= rho;
-    { const float m = __ldg(Mr + 4) * rp;
-      L[0] = fmaf(D[4], m, L[0]);
-      L[1] = fmaf(D[10], m, L[1]);
-      L[2] = fmaf(D[11], m, L[2]);
-      L[3] = fmaf(D[12], m, L[3]);
-    }
-    { const float m = __ldg(Mr + 5) * rp;
-      L[0] = fmaf(D[5], m, L[0]);
-      L[1] = fmaf(D[11], m, L[1]);
-      L[2] = fmaf(D[13], m, L[2]);
-      L[3] = fmaf(D[14], m, L[3]);
-    }
-    { const float m = __ldg(Mr + 6) * rp;
-      L[0] = fmaf(D[6], m, L[0]);
-      L[1] = fmaf(D[12], m, L[1]);
-      L[2] = fmaf(D[14], m, L[2]);
-      L[3] = fmaf(D[15], m, L[3]);
-    }
-    { const float m = __ldg(Mr + 7) * rp;
-      L[0] = fmaf(D[7], m, L[0]);
-      L[1] = fmaf(D[13], m, L[1]);
-      L[2] = fmaf(D[16], m, L[2]);
-      L[3] = fmaf(D[17], m, L[3]);
-    }
-    { const float m = __ldg(Mr + 8) * rp;
-      L[0] = fmaf(D[8], m, L[0]);
-      L[1] = fmaf(D[14], m, L[1]);
-      L[2] = fmaf(D[17], m, L[2]);
-      L[3] = fmaf(D[18], m, L[3]);
+    { const T m = -__ldg(Mr + 3) * rp;
+      L[0] = m2l_fma(D[3], m, L[0]);
+      L[1] = m2l_fma(D[6], m, L[1]);
+      L[2] = m2l_fma(D[8], m, L[2]);
+      L[3] = m2l_fma(D[9], m, L[3]);
+      L[4] = m2l_fma(D[12], m, L[4]);
+      L[5] = m2l_fma(D[14], m, L[5]);
+      L[6] = m2l_fma(D[15], m, L[6]);
+      L[7] = m2l_fma(D[17], m, L[7]);
+      L[8] = m2l_fma(D[18], m, L[8]);
     }
     rp *= rho;
-    { const float m = -__ldg(Mr + 9) * rp;
-      L[0] = fmaf(D[10], m, L[0]);
+    { const T m = __ldg(Mr + 4) * rp;
+      L[0] = m2l_fma(D[4], m, L[0]);
+      L[1] = m2l_fma(D[10], m, L[1]);
+      L[2] = m2l_fma(D[11], m, L[2]);
+      L[3] = m2l_fma(D[12], m, L[3]);
     }
-    { const float m = -__ldg(Mr + 10) * rp;
-      L[0] = fmaf(D[11], m, L[0]);
+    { const T m = __ldg(Mr + 5) * rp;
+      L[0] = m2l_fma(D[5], m, L[0]);
+      L[1] = m2l_fma(D[11], m, L[1]);
+      L[2] = m2l_fma(D[13], m, L[2]);
+      L[3] = m2l_fma(D[14], m, L[3]);
     }
-    { const float m = -__ldg(Mr + 11) * rp;
-      L[0] = fmaf(D[12], m, L[0]);
+    { const T m = __ldg(Mr + 6) * rp;
+      L[0] = m2l_fma(D[6], m, L[0]);
+      L[1] = m2l_fma(D[12], m, L[1]);
+      L[2] = m2l_fma(D[14], m, L[2]);
+      L[3] = m2l_fma(D[15], m, L[3]);
     }
-    { const float m = -__ldg(Mr + 12) * rp;
-      L[0] = fmaf(D[13], m, L[0]);
+    { const T m = __ldg(Mr + 7) * rp;
+      L[0] = m2l_fma(D[7], m, L[0]);
+      L[1] = m2l_fma(D[13], m, L[1]);
+      L[2] = m2l_fma(D[16], m, L[2]);
+      L[3] = m2l_fma(D[17], m, L[3]);
     }
-    { const float m = -__ldg(Mr + 13) * rp;
-      L[0] = fmaf(D[14], m, L[0]);
+    { const T m = __ldg(Mr + 8) * rp;
+      L[0] = m2l_fma(D[8], m, L[0]);
+      L[1] = m2l_fma(D[14], m, L[1]);
+      L[2] = m2l_fma(D[17], m, L[2]);
+      L[3] = m2l_fma(D[18], m, L[3]);
     }
-    { const float m = -__ldg(Mr + 14) * rp;
-      L[0] = fmaf(D[16], m, L[0]);
+    rp *= rho;
+    { const T m = -__ldg(Mr + 9) * rp;
+      L[0] = m2l_fma(D[10], m, L[0]);
     }
-    { const float m = -__ldg(Mr + 15) * rp;
-      L[0] = fmaf(D[17], m, L[0]);
+    { const T m = -__ldg(Mr + 10) * rp;
+      L[0] = m2l_fma(D[11], m, L[0]);
+    }
+    { const T m = -__ldg(Mr + 11) * rp;
+      L[0] = m2l_fma(D[12], m, L[0]);
+    }
+    { const T m = -__ldg(Mr + 12) * rp;
+      L[0] = m2l_fma(D[13], m, L[0]);
+    }
+    { const T m = -__ldg(Mr + 13) * rp;
+      L[0] = m2l_fma(D[14], m, L[0]);
+    }
+    { const T m = -__ldg(Mr + 14) * rp;
+      L[0] = m2l_fma(D[16], m, L[0]);
+    }
+    { const T m = -__ldg(Mr + 15) * rp;
+      L[0] = m2l_fma(D[17], m, L[0]);
     }
 }
 
-__device__ __forceinline__ void m2l_side_b_h_3(const float (&D)[19], const float *__restrict__ Mr, float (&L)[16])
+template <class T> __device__ __forceinline__ void m2l_side_b_h_3(const T (&D)[19], const T *__restrict__ Mr, T (&L)[16])
 {
-    { const float m = __ldg(Mr + 0);
+    { const T m = __ldg(Mr + 0);
       L[0] = D[0] * m;
       L[1] = -D[1] * m;
       L[2] = -D[2] * m;
@@ -9481,97 +9483,97 @@ __device__ __forceinline__ void m2l_side_b_h_3(const float (&D)[19], const float
       L[14] = -D[16] * m;
       L[15] = -D[17] * m;
     }
-    { const float m = __ldg(Mr + 1);
-      L[0] = fmaf(D[1], m, L[0]);
-      L[1] = fmaf(-D[4], m, L[1]);
-      L[2] = fmaf(-D[5], m, L[2]);
-      L[3] = fmaf(-D[6], m, L[3]);
-      L[4] = fmaf(D[10], m, L[4]);
-      L[5] = fmaf(D[11], m, L[5]);
-      L[6] = fmaf(D[12], m, L[6]);
-      L[7] = fmaf(D[13], m, L[7]);
-      L[8] = fmaf(D[14], m, L[8]);
+    { const T m = __ldg(Mr + 1);
+      L[0] = m2l_fma(D[1], m, L[0]);
+      L[1] = m2l_fma(-D[4], m, L[1]);
+      L[2] = m2l_fma(-D[5], m, L[2]);
+      L[3] = m2l_fma(-D[6], m, L[3]);
+      L[4] = m2l_fma(D[10], m, L[4]);
+      L[5] = m2l_fma(D[11], m, L[5]);
+      L[6] = m2l_fma(D[12], m, L[6]);
+      L[7] = m2l_fma(D[13], m, L[7]);
+      L[8] = m2l_fma(D[14], m, L[8]);
     }
-    { const float m = __ldg(Mr + 2);
-      L[0] = fmaf(D[2], m, L[0]);
-      L[1] = fmaf(-D[5], m, L[1]);
-      L[2] = fmaf(-D[7], m, L[2]);
-      L[3] = fmaf(-D[8], m, L[3]);
-      L[4] = fmaf(D[11], m, L[4]);
-      L[5] = fmaf(D[13], m, L[5]);
-      L[6] = fmaf(D[14], m, L[6]);
-      L[7] = fmaf(D[16], m, L[7]);
-      L[8] = fmaf(D[17], m, L[8]);
+    { const T m = __ldg(Mr + 2);
+      L[0] = m2l_fma(D[2], m, L[0]);
+      L[1] = m2l_fma(-D[5], m, L[1]);
+      L[2] = m2l_fma(-D[7], m, L[2]);
+      L[3] = m2l_fma(-D[8], m, L[3]);
+      L[4] = m2l_fma(D[11], m, L[4]);
+      L[5] = m2l_fma(D[13], m, L[5]);
+      L[6] = m2l_fma(D[14], m, L[6]);
+      L[7] = m2l_fma(D[16], m, L[7]);
+      L[8] = m2l_fma(D[17], m, L[8]);
     }
-    { const float m = __ldg(Mr + 3);
-      L[0] = fmaf(D[3], m, L[0]);
-      L[1] = fmaf(-D[6], m, L[1]);
-      L[2] = fmaf(-D[8], m, L[2]);
-      L[3] = fmaf(-D[9], m, L[3]);
-      L[4] = fmaf(D[12], m, L[4]);
-      L[5] = fmaf(D[14], m, L[5]);
-      L[6] = fmaf(D[15], m, L[6]);
-      L[7] = fmaf(D[17], m, L[7]);
-      L[8] = fmaf(D[18], m, L[8]);
+    { const T m = __ldg(Mr + 3);
+      L[0] = m2l_fma(D[3], m, L[0]);
+      L[1] = m2l_fma(-D[6], m, L[1]);
+      L[2] = m2l_fma(-D[8], m, L[2]);
+      L[3] = m2l_fma(-D[9], m, L[3]);
+      L[4] = m2l_fma(D[12], m, L[4]);
+      L[5] = m2l_fma(D[14], m, L[5]);
+      L[6] = m2l_fma(D[15], m, L[6]);
+      L[7] = m2l_fma(D[17], m, L[7]);
+      L[8] = m2l_fma(D[18], m, L[8]);
     }
-    { const float m = __ldg(Mr + 4);
-      L[0] = fmaf(D[4], m, L[0]);
-      L[1] = fmaf(-D[10], m, L[1]);
-      L[2] = fmaf(-D[11], m, L[2]);
-      L[3] = fmaf(-D[12], m, L[3]);
+    { const T m = __ldg(Mr + 4);
+      L[0] = m2l_fma(D[4], m, L[0]);
+      L[1] = m2l_fma(-D[10], m, L[1]);
+      L[2] = m2l_fma(-D[11], m, L[2]);
+      L[3] = m2l_fma(-D[12], m, L[3]);
     }
-    { const float m = __ldg(Mr + 5);
-      L[0] = fmaf(D[5], m, L[0]);
-      L[1] = fmaf(-D[11], m, L[1]);
-      L[2] = fmaf(-D[13], m, L[2]);
-      L[3] = fmaf(-D[14], m, L[3]);
+    { const T m = __ldg(Mr + 5);
+      L[0] = m2l_fma(D[5], m, L[0]);
+      L[1] = m2l_fma(-D[11], m, L[1]);
+      L[2] = m2l_fma(-D[13], m, L[2]);
+      L[3] = m2l_fma(-D[14], m, L[3]);
     }
-    { const float m = __ldg(Mr + 6);
-      L[0] = fmaf(D[6], m, L[0]);
-      L[1] = fmaf(-D[12], m, L[1]);
-      L[2] = fmaf(-D[14], m, L[2]);
-      L[3] = fmaf(-D[15], m, L[3]);
+    { const T m = __ldg(Mr + 6);
+      L[0] = m2l_fma(D[6], m, L[0]);
+      L[1] = m2l_fma(-D[12], m, L[1]);
+      L[2] = m2l_fma(-D[14], m, L[2]);
+      L[3] = m2l_fma(-D[15], m, L[3]);
     }
-    { const float m = __ldg(Mr + 7);
-      L[0] = fmaf(D[7], m, L[0]);
-      L[1] = fmaf(-D[13], m, L[1]);
-      L[2] = fmaf(-D[16], m, L[2]);
-      L[3] = fmaf(-D[17], m, L[3]);
+    { const T m = __ldg(Mr + 7);
+      L[0] = m2l_fma(D[7], m, L[0]);
+      L[1] = m2l_fma(-D[13], m, L[1]);
+      L[2] = m2l_fma(-D[16], m, L[2]);
+      L[3] = m2l_fma(-D[17], m, L[3]);
     }
-    { const float m = __ldg(Mr + 8);
-      L[0] = fmaf(D[8], m, L[0]);
-      L[1] = fmaf(-D[14], m, L[1]);
-      L[2] = fmaf(-D[17], m, L[2]);
-      L[3] = fmaf(-D[18], m, L[3]);
+    { const T m = __ldg(Mr + 8);
+      L[0] = m2l_fma(D[8], m, L[0]);
+      L[1] = m2l_fma(-D[14], m, L[1]);
+      L[2] = m2l_fma(-D[17], m, L[2]);
+      L[3] = m2l_fma(-D[18], m, L[3]);
     }
-    { const float m = __ldg(Mr + 9);
-      L[0] = fmaf(D[10], m, L[0]);
+    { const T m = __ldg(Mr + 9);
+      L[0] = m2l_fma(D[10], m, L[0]);
     }
-    { const float m = __ldg(Mr + 10);
-      L[0] = fmaf(D[11], m, L[0]);
+    { const T m = __ldg(Mr + 10);
+      L[0] = m2l_fma(D[11], m, L[0]);
     }
-    { const float m = __ldg(Mr + 11);
-      L[0] = fmaf(D[12], m, L[0]);
+    { const T m = __ldg(Mr + 11);
+      L[0] = m2l_fma(D[12], m, L[0]);
     }
-    { const float m = __ldg(Mr + 12);
-      L[0] = fmaf(D[13], m, L[0]);
+    { const T m = __ldg(Mr + 12);
+      L[0] = m2l_fma(D[13], m, L[0]);
     }
-    { const float m = __ldg(Mr + 13);
-      L[0] = fmaf(D[14], m, L[0]);
+    { const T m = __ldg(Mr + 13);
+      L[0] = m2l_fma(D[14], m, L[0]);
     }
-    { const float m = __ldg(Mr + 14);
-      L[0] = fmaf(D[16], m, L[0]);
+    { const T m = __ldg(Mr + 14);
+      L[0] = m2l_fma(D[16], m, L[0]);
     }
-    { const float m = __ldg(Mr + 15);
-      L[0] = fmaf(D[17], m, L[0]);
+    { const T m = __ldg(Mr + 15);
+      L[0] = m2l_fma(D[17], m, L[0]);
     }
 }
 
-__device__ __forceinline__ void m2l_side_a_h_forces_3(const float (&D)[19], const float *__restrict__ Mr, float rho, float (&L)[16])
+template <class T> __device__ __forceinline__ void m2l_side_a_h_forces_3(const T (&D)[19], const T *__restrict__ Mr, T rho, T (&L)[16])
 {
-    L[0] = 0.0f;
-    float rp = 1.0f;
-    { const float m = __ldg(Mr + 0) * rp;
+    L[0] = T(0);
+    T rp = T(1);
+    { const T m = __ldg(Mr + 0) * rp;
       L[1] = D[1] * m;
       L[2] = D[2] * m;
       L[3] = D[3] * m;
@@ -9589,147 +9591,147 @@ __device__ __forceinline__ void m2l_side_a_h_forces_3(const float (&D)[19], cons
       L[15] = D[17] * m;
     }
     rp *= rho;
-    { const float m = -__ldg(Mr + 1) * rp;
-      L[1] = fmaf(D[4], m, L[1]);
-      L[2] = fmaf(D[5], m, L[2]);
-      L[3] = fmaf(D[6], m, L[3]);
-      L[4] = fmaf(D[10], m, L[4]);
-      L[5] = fmaf(D[11], m, L[5]);
-      L[6] = fmaf(D[12], m, L[6]);
-      L[7] = fmaf(D[13], m, L[7]);
-      L[8] = fmaf(D[14], m, L[8]);
+    { const T m = -__ldg(Mr + 1) * rp;
+      L[1] = m2l_fma(D[4], m, L[1]);
+      L[2] = m2l_fma(D[5], m, L[2]);
+      L[3] = m2l_fma(D[6], m, L[3]);
+      L[4] = m2l_fma(D[10], m, L[4]);
+      L[5] = m2l_fma(D[11], m, L[5]);
+      L[6] = m2l_fma(D[12], m, L[6]);
+      L[7] = m2l_fma(D[13], m, L[7]);
+      L[8] = m2l_fma(D[14], m, L[8]);
     }
-    { const float m = -__ldg(Mr + 2) * rp;
-      L[1] = fmaf(D[5], m, L[1]);
-      L[2] = fmaf(D[7], m, L[2]);
-      L[3] = fmaf(D[8], m, L[3]);
-      L[4] = fmaf(D[11], m, L[4]);
-      L[5] = fmaf(D[13], m, L[5]);
-      L[6] = fmaf(D[14], m, L[6]);
-      L[7] = fmaf(D[16], m, L[7]);
-      L[8] = fmaf(D[17], m, L[8]);
+    { const T m = -__ldg(Mr + 2) * rp;
+      L[1] = m2l_fma(D[5], m, L[1]);
+      L[2] = m2l_fma(D[7], m, L[2]);
+      L[3] = m2l_fma(D[8], m, L[3]);
+      L[4] = m2l_fma(D[11], m, L[4]);
+      L[5] = m2l_fma(D[13], m, L[5]);
+      L[6] = m2l_fma(D[14], m, L[6]);
+      L[7] = m2l_fma(D[16], m, L[7]);
+      L[8] = m2l_fma(D[17], m, L[8]);
     }
-    { const float m = -__ldg(Mr + 3) * rp;
-      L[1] = fmaf(D[6], m, L[1]);
-      L[2] = fmaf(D[8], m, L[2]);
-      L[3] = fmaf(D[9], m, L[3]);
-      L[4] = fmaf(D[12], m, L[4]);
-      L[5] = fmaf(D[14], m, L[5]);
-      L[6] = fmaf(D[15], m, L[6]);
-      L[7] = fmaf(D[17], m, L[7]);
-      L[8] = fmaf(D[18], m, L[8]);
+    { const T m = -__ldg(Mr + 3) * rp;
+      L[1] = m2l_fma(D[6], m, L[1]);
+      L[2] = m2l_fma(D[8], m, L[2]);
+      L[3] = m2l_fma(D[9], m, L[3]);
+      L[4] = m2l_fma(D[12], m, L[4]);
+      L[5] = m2l_fma(D[14], m, L[5]);
+      L[6] = m2l_fma(D[15], m, L[6]);
+      L[7] = m2l_fma(D[17], m, L[7]);
+      L[8] = m2l_fma(D[18], m, L[8]);
     }
     rp *= rho;
-    { const float m = __ldg(Mr + 4) * rp;
-      L[1] = fmaf(D[10], m, L[1]);
-      L[2] = fmaf(D[11], m, L[2]);
-      L[3] = fmaf(D[12], m, L[3]);
+    { const T m = __ldg(Mr + 4) * rp;
+      L[1] = m2l_fma(D[10], m, L[1]);
+      L[2] = m2l_fma(D[11], m, L[2]);
+      L[3] = m2l_fma(D[12], m, L[3]);
     }
-    { const float m = __ldg(Mr + 5) * rp;
-      L[1] = fmaf(D[11], m, L[1]);
-      L[2] = fmaf(D[13], m, L[2]);
-      L[3] = fmaf(D[14], m, L[3]);
+    { const T m = __ldg(Mr + 5) * rp;
+      L[1] = m2l_fma(D[11], m, L[1]);
+      L[2] = m2l_fma(D[13], m, L[2]);
+      L[3] = m2l_fma(D[14], m, L[3]);
     }
-    { const float m = __ldg(Mr + 6) * rp;
-      L[1] = fmaf(D[12], m, L[1]);
-      L[2] = fmaf(D[14], m, L[2]);
-      L[3] = fmaf(D[15], m, L[3]);
+    { const T m = __ldg(Mr + 6) * rp;
+      L[1] = m2l_fma(D[12], m, L[1]);
+      L[2] = m2l_fma(D[14], m, L[2]);
+      L[3] = m2l_fma(D[15], m, L[3]);
     }
-    { const float m = __ldg(Mr + 7) * rp;
-      L[1] = fmaf(D[13], m, L[1]);
-      L[2] = fmaf(D[16], m, L[2]);
-      L[3] = fmaf(D[17], m, L[3]);
+    { const T m = __ldg(Mr + 7) * rp;
+      L[1] = m2l_fma(D[13], m, L[1]);
+      L[2] = m2l_fma(D[16], m, L[2]);
+      L[3] = m2l_fma(D[17], m, L[3]);
     }
-    { const float m = __ldg(Mr + 8) * rp;
-      L[1] = fmaf(D[14], m, L[1]);
-      L[2] = fmaf(D[17], m, L[2]);
-      L[3] = fmaf(D[18], m, L[3]);
+    { const T m = __ldg(Mr + 8) * rp;
+      L[1] = m2l_fma(D[14], m, L[1]);
+      L[2] = m2l_fma(D[17], m, L[2]);
+      L[3] = m2l_fma(D[18], m, L[3]);
     }
 }
 
-__device__ __forceinline__ void m2l_acc_h_forces_3(const float (&D)[19], const float *__restrict__ Mr, float rho, float (&L)[16])
+template <class T> __device__ __forceinline__ void m2l_acc_h_forces_3(const T (&D)[19], const T *__restrict__ Mr, T rho, T (&L)[16])
 {
-    float rp = 1.0f;
-    { const float m = __ldg(Mr + 0) * rp;
-      L[1] = fmaf(D[1], m, L[1]);
-      L[2] = fmaf(D[2], m, L[2]);
-      L[3] = fmaf(D[3], m, L[3]);
-      L[4] = fmaf(D[4], m, L[4]);
-      L[5] = fmaf(D[5], m, L[5]);
-      L[6] = fmaf(D[6], m, L[6]);
-      L[7] = fmaf(D[7], m, L[7]);
-      L[8] = fmaf(D[8], m, L[8]);
-      L[9] = fmaf(D[10], m, L[9]);
-      L[10] = fmaf(D[11], m, L[10]);
-      L[11] = fmaf(D[12], m, L[11]);
-      L[12] = fmaf(D[13], m, L[12]);
-      L[13] = fmaf(D[14], m, L[13]);
-      L[14] = fmaf(D[16], m, L[14]);
-      L[15] = fmaf(D[17], m, L[15]);
+    T rp = T(1);
+    { const T m = __ldg(Mr + 0) * rp;
+      L[1] = m2l_fma(D[1], m, L[1]);
+      L[2] = m2l_fma(D[2], m, L[2]);
+      L[3] = m2l_fma(D[3], m, L[3]);
+      L[4] = m2l_fma(D[4], m, L[4]);
+      L[5] = m2l_fma(D[5], m, L[5]);
+      L[6] = m2l_fma(D[6], m, L[6]);
+      L[7] = m2l_fma(D[7], m, L[7]);
+      L[8] = m2l_fma(D[8], m, L[8]);
+      L[9] = m2l_fma(D[10], m, L[9]);
+      L[10] = m2l_fma(D[11], m, L[10]);
+      L[11] = m2l_fma(D[12], m, L[11]);
+      L[12] = m2l_fma(D[13], m, L[12]);
+      L[13] = m2l_fma(D[14], m, L[13]);
+      L[14] = m2l_fma(D[16], m, L[14]);
+      L[15] = m2l_fma(D[17], m, L[15]);
     }
     rp *= rho;
-    { const float m = -__ldg(Mr + 1) * rp;
-      L[1] = fmaf(D[4], m, L[1]);
-      L[2] = fmaf(D[5], m, L[2]);
-      L[3] = fmaf(D[6], m, L[3]);
-      L[4] = fmaf(D[10], m, L[4]);
-      L[5] = fmaf(D[11], m, L[5]);
-      L[6] = fmaf(D[12], m, L[6]);
-      L[7] = fmaf(D[13], m, L[7]);
-      L[8] = fmaf(D[14], m, L[8]);
+    { const T m = -__ldg(Mr + 1) * rp;
+      L[1] = m2l_fma(D[4], m, L[1]);
+      L[2] = m2l_fma(D[5], m, L[2]);
+      L[3] = m2l_fma(D[6], m, L[3]);
+      L[4] = m2l_fma(D[10], m, L[4]);
+      L[5] = m2l_fma(D[11], m, L[5]);
+      L[6] = m2l_fma(D[12], m, L[6]);
+      L[7] = m2l_fma(D[13], m, L[7]);
+      L[8] = m2l_fma(D[14], m, L[8]);
     }
-    { const float m = -__ldg(Mr + 2) * rp;
-      L[1] = fmaf(D[5], m, L[1]);
-      L[2] = fmaf(D[7], m, L[2]);
-      L[3] = fmaf(D[8], m, L[3]);
-      L[4] = fmaf(D[11], m, L[4]);
-      L[5] = fmaf(D[13], m, L[5]);
-      L[6] = fmaf(D[14], m, L[6]);
-      L[7] = fmaf(D[16], m, L[7]);
-      L[8] = fmaf(D[17], m, L[8]);
+    { const T m = -__ldg(Mr + 2) * rp;
+      L[1] = m2l_fma(D[5], m, L[1]);
+      L[2] = m2l_fma(D[7], m, L[2]);
+      L[3] = m2l_fma(D[8], m, L[3]);
+      L[4] = m2l_fma(D[11], m, L[4]);
+      L[5] = m2l_fma(D[13], m, L[5]);
+      L[6] = m2l_fma(D[14], m, L[6]);
+      L[7] = m2l_fma(D[16], m, L[7]);
+      L[8] = m2l_fma(D[17], m, L[8]);
     }
-    { const float m = -__ldg(Mr + 3) * rp;
-      L[1] = fmaf(D[6], m, L[1]);
-      L[2] = fmaf(D[8], m, L[2]);
-      L[3] = fmaf(D[9], m, L[3]);
-      L[4] = fmaf(D[12], m, L[4]);
-      L[5] = fmaf(D[14], m, L[5]);
-      L[6] = fmaf(D[15], m, L[6]);
-      L[7] = fmaf(D[17], m, L[7]);
-      L[8] = fmaf(D[18], m, L[8]);
+    { const T m = -__ldg(Mr + 3) * rp;
+      L[1] = m2l_fma(D[6], m, L[1]);
+      L[2] = m2l_fma(D[8], m, L[2]);
+      L[3] = m2l_fma(D[9], m, L[3]);
+      L[4] = m2l_fma(D[12], m, L[4]);
+      L[5] = m2l_fma(D[14], m, L[5]);
+      L[6] = m2l_fma(D[15], m, L[6]);
+      L[7] = m2l_fma(D[17], m, L[7]);
+      L[8] = m2l_fma(D[18], m, L[8]);
     }
     rp *= rho;
-    { const float m = __ldg(Mr + 4) * rp;
-      L[1] = fmaf(D[10], m, L[1]);
-      L[2] = fmaf(D[11], m, L[2]);
-      L[3] = fmaf(D[12], m, L[3]);
+    { const T m = __ldg(Mr + 4) * rp;
+      L[1] = m2l_fma(D[10], m, L[1]);
+      L[2] = m2l_fma(D[11], m, L[2]);
+      L[3] = m2l_fma(D[12], m, L[3]);
     }
-    { const float m = __ldg(Mr + 5) * rp;
-      L[1] = fmaf(D[11], m, L[1]);
-      L[2] = fmaf(D[13], m, L[2]);
-      L[3] = fmaf(D[14], m, L[3]);
+    { const T m = __ldg(Mr + 5) * rp;
+      L[1] = m2l_fma(D[11], m, L[1]);
+      L[2] = m2l_fma(D[13], m, L[2]);
+      L[3] = m2l_fma(D[14], m, L[3]);
     }
-    { const float m = __ldg(Mr + 6) * rp;
-      L[1] = fmaf(D[12], m, L[1]);
-      L[2] = fmaf(D[14], m, L[2]);
-      L[3] = fmaf(D[15], m, L[3]);
+    { const T m = __ldg(Mr + 6) * rp;
+      L[1] = m2l_fma(D[12], m, L[1]);
+      L[2] = m2l_fma(D[14], m, L[2]);
+      L[3] = m2l_fma(D[15], m, L[3]);
     }
-    { const float m = __ldg(Mr + 7) * rp;
-      L[1] = fmaf(D[13], m, L[1]);
-      L[2] = fmaf(D[16], m, L[2]);
-      L[3] = fmaf(D[17], m, L[3]);
+    { const T m = __ldg(Mr + 7) * rp;
+      L[1] = m2l_fma(D[13], m, L[1]);
+      L[2] = m2l_fma(D[16], m, L[2]);
+      L[3] = m2l_fma(D[17], m, L[3]);
     }
-    { const float m = __ldg(Mr + 8) * rp;
-      L[1] = fmaf(D[14], m, L[1]);
-      L[2] = fmaf(D[17], m, L[2]);
-      L[3] = fmaf(D[18], m, L[3]);
+    { const T m = __ldg(Mr + 8) * rp;
+      L[1] = m2l_fma(D[14], m, L[1]);
+      L[2] = m2l_fma(D[17], m, L[2]);
+      L[3] = m2l_fma(D[18], m, L[3]);
     }
 }
 
-__device__ __forceinline__ void m2l_side_b_h_forces_3(const float (&D)[19], const float *__restrict__ Mr, float (&L)[16])
+template <class T> __device__ __forceinline__ void m2l_side_b_h_forces_3(const T (&D)[19], const T *__restrict__ Mr, T (&L)[16])
 {
-    L[0] = 0.0f;
-    { const float m = __ldg(Mr + 0);
+    L[0] = T(0);
+    { const T m = __ldg(Mr + 0);
       L[1] = -D[1] * m;
       L[2] = -D[2] * m;
       L[3] = -D[3] * m;
@@ -9746,85 +9748,85 @@ __device__ __forceinline__ void m2l_side_b_h_forces_3(const float (&D)[19], cons
       L[14] = -D[16] * m;
       L[15] = -D[17] * m;
     }
-    { const float m = __ldg(Mr + 1);
-      L[1] = fmaf(-D[4], m, L[1]);
-      L[2] = fmaf(-D[5], m, L[2]);
-      L[3] = fmaf(-D[6], m, L[3]);
-      L[4] = fmaf(D[10], m, L[4]);
-      L[5] = fmaf(D[11], m, L[5]);
-      L[6] = fmaf(D[12], m, L[6]);
-      L[7] = fmaf(D[13], m, L[7]);
-      L[8] = fmaf(D[14], m, L[8]);
+    { const T m = __ldg(Mr + 1);
+      L[1] = m2l_fma(-D[4], m, L[1]);
+      L[2] = m2l_fma(-D[5], m, L[2]);
+      L[3] = m2l_fma(-D[6], m, L[3]);
+      L[4] = m2l_fma(D[10], m, L[4]);
+      L[5] = m2l_fma(D[11], m, L[5]);
+      L[6] = m2l_fma(D[12], m, L[6]);
+      L[7] = m2l_fma(D[13], m, L[7]);
+      L[8] = m2l_fma(D[14], m, L[8]);
     }
-    { const float m = __ldg(Mr + 2);
-      L[1] = fmaf(-D[5], m, L[1]);
-      L[2] = fmaf(-D[7], m, L[2]);
-      L[3] = fmaf(-D[8], m, L[3]);
-      L[4] = fmaf(D[11], m, L[4]);
-      L[5] = fmaf(D[13], m, L[5]);
-      L[6] = fmaf(D[14], m, L[6]);
-      L[7] = fmaf(D[16], m, L[7]);
-      L[8] = fmaf(D[17], m, L[8]);
+    { const T m = __ldg(Mr + 2);
+      L[1] = m2l_fma(-D[5], m, L[1]);
+      L[2] = m2l_fma(-D[7], m, L[2]);
+      L[3] = m2l_fma(-D[8], m, L[3]);
+      L[4] = m2l_fma(D[11], m, L[4]);
+      L[5] = m2l_fma(D[13], m, L[5]);
+      L[6] = m2l_fma(D[14], m, L[6]);
+      L[7] = m2l_fma(D[16], m, L[7]);
+      L[8] = m2l_fma(D[17], m, L[8]);
     }
-    { const float m = __ldg(Mr + 3);
-      L[1] = fmaf(-D[6], m, L[1]);
-      L[2] = fmaf(-D[8], m, L[2]);
-      L[3] = fmaf(-D[9], m, L[3]);
-      L[4] = fmaf(D[12], m, L[4]);
-      L[5] = fmaf(D[14], m, L[5]);
-      L[6] = fmaf(D[15], m, L[6]);
-      L[7] = fmaf(D[17], m, L[7]);
-      L[8] = fmaf(D[18], m, L[8]);
+    { const T m = __ldg(Mr + 3);
+      L[1] = m2l_fma(-D[6], m, L[1]);
+      L[2] = m2l_fma(-D[8], m, L[2]);
+      L[3] = m2l_fma(-D[9], m, L[3]);
+      L[4] = m2l_fma(D[12], m, L[4]);
+      L[5] = m2l_fma(D[14], m, L[5]);
+      L[6] = m2l_fma(D[15], m, L[6]);
+      L[7] = m2l_fma(D[17], m, L[7]);
+      L[8] = m2l_fma(D[18], m, L[8]);
     }
-    { const float m = __ldg(Mr + 4);
-      L[1] = fmaf(-D[10], m, L[1]);
-      L[2] = fmaf(-D[11], m, L[2]);
-      L[3] = fmaf(-D[12], m, L[3]);
+    { const T m = __ldg(Mr + 4);
+      L[1] = m2l_fma(-D[10], m, L[1]);
+      L[2] = m2l_fma(-D[11], m, L[2]);
+      L[3] = m2l_fma(-D[12], m, L[3]);
     }
-    { const float m = __ldg(Mr + 5);
-      L[1] = fmaf(-D[11], m, L[1]);
-      L[2] = fmaf(-D[13], m, L[2]);
-      L[3] = fmaf(-D[14], m, L[3]);
+    { const T m = __ldg(Mr + 5);
+      L[1] = m2l_fma(-D[11], m, L[1]);
+      L[2] = m2l_fma(-D[13], m, L[2]);
+      L[3] = m2l_fma(-D[14], m, L[3]);
     }
-    { const float m = __ldg(Mr + 6);
-      L[1] = fmaf(-D[12], m, L[1]);
-      L[2] = fmaf(-D[14], m, L[2]);
-      L[3] = fmaf(-D[15], m, L[3]);
+    { const T m = __ldg(Mr + 6);
+      L[1] = m2l_fma(-D[12], m, L[1]);
+      L[2] = m2l_fma(-D[14], m, L[2]);
+      L[3] = m2l_fma(-D[15], m, L[3]);
     }
-    { const float m = __ldg(Mr + 7);
-      L[1] = fmaf(-D[13], m, L[1]);
-      L[2] = fmaf(-D[16], m, L[2]);
-      L[3] = fmaf(-D[17], m, L[3]);
+    { const T m = __ldg(Mr + 7);
+      L[1] = m2l_fma(-D[13], m, L[1]);
+      L[2] = m2l_fma(-D[16], m, L[2]);
+      L[3] = m2l_fma(-D[17], m, L[3]);
     }
-    { const float m = __ldg(Mr + 8);
-      L[1] = fmaf(-D[14], m, L[1]);
-      L[2] = fmaf(-D[17], m, L[2]);
-      L[3] = fmaf(-D[18], m, L[3]);
+    { const T m = __ldg(Mr + 8);
+      L[1] = m2l_fma(-D[14], m, L[1]);
+      L[2] = m2l_fma(-D[17], m, L[2]);
+      L[3] = m2l_fma(-D[18], m, L[3]);
     }
 }
 
-__device__ __forceinline__ void m2l_reduce_moments_h_3(const float *__restrict__ Ms, float *__restrict__ Mr)
+template <class T> __device__ __forceinline__ void m2l_reduce_moments_h_3(const T *__restrict__ Ms, T *__restrict__ Mr)
 {
-    float v0 = Ms[0];
-    float v1 = Ms[1];
-    float v2 = Ms[2];
-    float v3 = Ms[3];
-    float v4 = Ms[4];
-    float v5 = Ms[5];
-    float v6 = Ms[6];
-    float v7 = Ms[7];
-    float v8 = Ms[8];
-    float v9 = Ms[9];
-    float v10 = Ms[10];
-    float v11 = Ms[11];
-    float v12 = Ms[12];
-    float v13 = Ms[13];
-    float v14 = Ms[14];
-    float v15 = Ms[15];
-    float v16 = Ms[16];
-    float v17 = Ms[17];
-    float v18 = Ms[18];
-    float v19 = Ms[19];
+    T v0 = Ms[0];
+    T v1 = Ms[1];
+    T v2 = Ms[2];
+    T v3 = Ms[3];
+    T v4 = Ms[4];
+    T v5 = Ms[5];
+    T v6 = Ms[6];
+    T v7 = Ms[7];
+    T v8 = Ms[8];
+    T v9 = Ms[9];
+    T v10 = Ms[10];
+    T v11 = Ms[11];
+    T v12 = Ms[12];
+    T v13 = Ms[13];
+    T v14 = Ms[14];
+    T v15 = Ms[15];
+    T v16 = Ms[16];
+    T v17 = Ms[17];
+    T v18 = Ms[18];
+    T v19 = Ms[19];
     v12 -= v19;
     v17 -= v19;
     v4 -= v9;
@@ -9851,96 +9853,95 @@ __device__ __forceinline__ void m2l_reduce_moments_h_3(const float *__restrict__
     Mr[15] = v17;
 }
 
-__device__ __forceinline__ void m2l_complete_locals_h_3(const float *__restrict__ Lr, float *__restrict__ L)
+template <class T> __device__ __forceinline__ void m2l_complete_locals_h_3(const T *__restrict__ Lr, T *__restrict__ L)
 {
-    const float v0 = Lr[0];
+    const T v0 = Lr[0];
     L[0] = v0;
-    const float v1 = Lr[1];
+    const T v1 = Lr[1];
     L[1] = v1;
-    const float v2 = Lr[2];
+    const T v2 = Lr[2];
     L[2] = v2;
-    const float v3 = Lr[3];
+    const T v3 = Lr[3];
     L[3] = v3;
-    const float v4 = Lr[4];
+    const T v4 = Lr[4];
     L[4] = v4;
-    const float v5 = Lr[5];
+    const T v5 = Lr[5];
     L[5] = v5;
-    const float v6 = Lr[6];
+    const T v6 = Lr[6];
     L[6] = v6;
-    const float v7 = Lr[7];
+    const T v7 = Lr[7];
     L[7] = v7;
-    const float v8 = Lr[8];
+    const T v8 = Lr[8];
     L[8] = v8;
-    const float v9 = -v4 - v7;
+    const T v9 = -v4 - v7;
     L[9] = v9;
-    const float v10 = Lr[9];
+    const T v10 = Lr[9];
     L[10] = v10;
-    const float v11 = Lr[10];
+    const T v11 = Lr[10];
     L[11] = v11;
-    const float v12 = Lr[11];
+    const T v12 = Lr[11];
     L[12] = v12;
-    const float v13 = Lr[12];
+    const T v13 = Lr[12];
     L[13] = v13;
-    const float v14 = Lr[13];
+    const T v14 = Lr[13];
     L[14] = v14;
-    const float v15 = -v10 - v13;
+    const T v15 = -v10 - v13;
     L[15] = v15;
-    const float v16 = Lr[14];
+    const T v16 = Lr[14];
     L[16] = v16;
-    const float v17 = Lr[15];
+    const T v17 = Lr[15];
     L[17] = v17;
-    const float v18 = -v11 - v16;
+    const T v18 = -v11 - v16;
     L[18] = v18;
-    const float v19 = -v12 - v17;
+    const T v19 = -v12 - v17;
     L[19] = v19;
 }
 
-__device__ __forceinline__ void m2l_dtensor_h_4(float dx, float dy, float dz, float (&D)[31])
+template <class T> __device__ __forceinline__ void m2l_dtensor_h_4(T dx, T dy, T dz, T (&D)[31])
 {
-    const float s2 = fmaf(dx, dx, fmaf(dy, dy, dz * dz));
-    float si = rsqrtf(s2);
-    si = si * fmaf(-0.5f * s2, si * si, 1.5f);   // one Newton step
-    const float si2 = si * si;
-    const float f0 = -si;
-    const float f1 = -1.0f * f0 * si2;
-    const float f2 = -3.0f * f1 * si2;
-    const float f3 = -5.0f * f2 * si2;
-    const float f4 = -7.0f * f3 * si2;
-    const float r_0_0 = f0;
-    const float r_1_0 = f1;
-    const float r_2_0 = f2;
-    const float r_3_0 = f3;
-    const float r_4_0 = f4;
-    const float r_0_1 = dx * r_1_0;
-    const float r_1_1 = dx * r_2_0;
-    const float r_2_1 = dx * r_3_0;
-    const float r_3_1 = dx * r_4_0;
-    const float r_0_2 = dy * r_1_0;
-    const float r_1_2 = dy * r_2_0;
-    const float r_2_2 = dy * r_3_0;
-    const float r_3_2 = dy * r_4_0;
-    const float r_0_4 = fmaf(1.0f, r_1_0, dx * r_1_1);
-    const float r_1_4 = fmaf(1.0f, r_2_0, dx * r_2_1);
-    const float r_2_4 = fmaf(1.0f, r_3_0, dx * r_3_1);
-    const float r_0_5 = dx * r_1_2;
-    const float r_1_5 = dx * r_2_2;
-    const float r_2_5 = dx * r_3_2;
-    const float r_0_7 = fmaf(1.0f, r_1_0, dy * r_1_2);
-    const float r_1_7 = fmaf(1.0f, r_2_0, dy * r_2_2);
-    const float r_2_7 = fmaf(1.0f, r_3_0, dy * r_3_2);
-    const float r_0_10 = fmaf(2.0f, r_1_1, dx * r_1_4);
-    const float r_1_10 = fmaf(2.0f, r_2_1, dx * r_2_4);
-    const float r_0_11 = fmaf(1.0f, r_1_2, dx * r_1_5);
-    const float r_1_11 = fmaf(1.0f, r_2_2, dx * r_2_5);
-    const float r_0_13 = dx * r_1_7;
-    const float r_1_13 = dx * r_2_7;
-    const float r_0_16 = fmaf(2.0f, r_1_2, dy * r_1_7);
-    const float r_1_16 = fmaf(2.0f, r_2_2, dy * r_2_7);
-    const float r_0_20 = fmaf(3.0f, r_1_4, dx * r_1_10);
-    const float r_0_21 = fmaf(2.0f, r_1_5, dx * r_1_11);
-    const float r_0_23 = fmaf(1.0f, r_1_7, dx * r_1_13);
-    const float r_0_26 = dx * r_1_16;
-    const float r_0_30 = fmaf(3.0f, r_1_7, dy * r_1_16);
+    const T s2 = m2l_fma(dx, dx, m2l_fma(dy, dy, dz * dz));
+    const T si = m2l_rsqrt(s2);
+    const T si2 = si * si;
+    const T f0 = -si;
+    const T f1 = T(-1) * f0 * si2;
+    const T f2 = T(-3) * f1 * si2;
+    const T f3 = T(-5) * f2 * si2;
+    const T f4 = T(-7) * f3 * si2;
+    const T r_0_0 = f0;
+    const T r_1_0 = f1;
+    const T r_2_0 = f2;
+    const T r_3_0 = f3;
+    const T r_4_0 = f4;
+    const T r_0_1 = dx * r_1_0;
+    const T r_1_1 = dx * r_2_0;
+    const T r_2_1 = dx * r_3_0;
+    const T r_3_1 = dx * r_4_0;
+    const T r_0_2 = dy * r_1_0;
+    const T r_1_2 = dy * r_2_0;
+    const T r_2_2 = dy * r_3_0;
+    const T r_3_2 = dy * r_4_0;
+    const T r_0_4 = m2l_fma(T(1), r_1_0, dx * r_1_1);
+    const T r_1_4 = m2l_fma(T(1), r_2_0, dx * r_2_1);
+    const T r_2_4 = m2l_fma(T(1), r_3_0, dx * r_3_1);
+    const T r_0_5 = dx * r_1_2;
+    const T r_1_5 = dx * r_2_2;
+    const T r_2_5 = dx * r_3_2;
+    const T r_0_7 = m2l_fma(T(1), r_1_0, dy * r_1_2);
+    const T r_1_7 = m2l_fma(T(1), r_2_0, dy * r_2_2);
+    const T r_2_7 = m2l_fma(T(1), r_3_0, dy * r_3_2);
+    const T r_0_10 = m2l_fma(T(2), r_1_1, dx * r_1_4);
+    const T r_1_10 = m2l_fma(T(2), r_2_1, dx * r_2_4);
+    const T r_0_11 = m2l_fma(T(1), r_1_2, dx * r_1_5);
+    const T r_1_11 = m2l_fma(T(1), r_2_2, dx * r_2_5);
+    const T r_0_13 = dx * r_1_7;
+    const T r_1_13 = dx * r_2_7;
+    const T r_0_16 = m2l_fma(T(2), r_1_2, dy * r_1_7);
+    const T r_1_16 = m2l_fma(T(2), r_2_2, dy * r_2_7);
+    const T r_0_20 = m2l_fma(T(3), r_1_4, dx * r_1_10);
+    const T r_0_21 = m2l_fma(T(2), r_1_5, dx * r_1_11);
+    const T r_0_23 = m2l_fma(T(1), r_1_7, dx * r_1_13);
+    const T r_0_26 = dx * r_1_16;
+    const T r_0_30 = m2l_fma(T(3), r_1_7, dy * r_1_16);
     D[0] = r_0_0;
     D[1] = r_0_1;
     D[2] = r_0_2;
@@ -9974,10 +9975,10 @@ __device__ __forceinline__ void m2l_dtensor_h_4(float dx, float dy, float dz, fl
     D[30] = -D[22] - D[28];
 }
 
-__device__ __forceinline__ void m2l_side_a_h_4(const float (&D)[31], const float *__restrict__ Mr, float rho, float (&L)[25])
+template <class T> __device__ __forceinline__ void m2l_side_a_h_4(const T (&D)[31], const T *__restrict__ Mr, T rho, T (&L)[25])
 {
-    float rp = 1.0f;
-    { const float m = __ldg(Mr + 0) * rp;
+    T rp = T(1);
+    { const T m = __ldg(Mr + 0) * rp;
       L[0] = D[0] * m;
       L[1] = D[1] * m;
       L[2] = D[2] * m;
@@ -10005,406 +10006,406 @@ __device__ __forceinline__ void m2l_side_a_h_4(const float (&D)[31], const float
       L[24] = D[29] * m;
     }
     rp *= rho;
-    { const float m = -__ldg(Mr + 1) * rp;
-      L[0] = fmaf(D[1], m, L[0]);
-      L[1] = fmaf(D[4], m, L[1]);
-      L[2] = fmaf(D[5], m, L[2]);
-      L[3] = fmaf(D[6], m, L[3]);
-      L[4] = fmaf(D[10], m, L[4]);
-      L[5] = fmaf(D[11], m, L[5]);
-      L[6] = fmaf(D[12], m, L[6]);
-      L[7] = fmaf(D[13], m, L[7]);
-      L[8] = fmaf(D[14], m, L[8]);
-      L[9] = fmaf(D[19], m, L[9]);
-      L[10] = fmaf(D[20], m, L[10]);
-      L[11] = fmaf(D[21], m, L[11]);
-      L[12] = fmaf(D[22], m, L[12]);
-      L[13] = fmaf(D[23], m, L[13]);
-      L[14] = fmaf(D[25], m, L[14]);
-      L[15] = fmaf(D[26], m, L[15]);
+    { const T m = -__ldg(Mr + 1) * rp;
+      L[0] = m2l_fma(D[1], m, L[0]);
+      L[1] = m2l_fma(D[4], m, L[1]);
+      L[2] = m2l_fma(D[5], m, L[2]);
+      L[3] = m2l_fma(D[6], m, L[3]);
+      L[4] = m2l_fma(D[10], m, L[4]);
+      L[5] = m2l_fma(D[11], m, L[5]);
+      L[6] = m2l_fma(D[12], m, L[6]);
+      L[7] = m2l_fma(D[13], m, L[7]);
+      L[8] = m2l_fma(D[14], m, L[8]);
+      L[9] = m2l_fma(D[19], m, L[9]);
+      L[10] = m2l_fma(D[20], m, L[10]);
+      L[11] = m2l_fma(D[21], m, L[11]);
+      L[12] = m2l_fma(D[22], m, L[12]);
+      L[13] = m2l_fma(D[23], m, L[13]);
+      L[14] = m2l_fma(D[25], m, L[14]);
+      L[15] = m2l_fma(D[26], m, L[15]);
     }
-    { const float m = -__ldg(Mr + 2) * rp;
-      L[0] = fmaf(D[2], m, L[0]);
-      L[1] = fmaf(D[5], m, L[1]);
-      L[2] = fmaf(D[7], m, L[2]);
-      L[3] = fmaf(D[8], m, L[3]);
-      L[4] = fmaf(D[11], m, L[4]);
-      L[5] = fmaf(D[13], m, L[5]);
-      L[6] = fmaf(D[14], m, L[6]);
-      L[7] = fmaf(D[16], m, L[7]);
-      L[8] = fmaf(D[17], m, L[8]);
-      L[9] = fmaf(D[20], m, L[9]);
-      L[10] = fmaf(D[22], m, L[10]);
-      L[11] = fmaf(D[23], m, L[11]);
-      L[12] = fmaf(D[25], m, L[12]);
-      L[13] = fmaf(D[26], m, L[13]);
-      L[14] = fmaf(D[28], m, L[14]);
-      L[15] = fmaf(D[29], m, L[15]);
+    { const T m = -__ldg(Mr + 2) * rp;
+      L[0] = m2l_fma(D[2], m, L[0]);
+      L[1] = m2l_fma(D[5], m, L[1]);
+      L[2] = m2l_fma(D[7], m, L[2]);
+      L[3] = m2l_fma(D[8], m, L[3]);
+      L[4] = m2l_fma(D[11], m, L[4]);
+      L[5] = m2l_fma(D[13], m, L[5]);
+      L[6] = m2l_fma(D[14], m, L[6]);
+      L[7] = m2l_fma(D[16], m, L[7]);
+      L[8] = m2l_fma(D[17], m, L[8]);
+      L[9] = m2l_fma(D[20], m, L[9]);
+      L[10] = m2l_fma(D[22], m, L[10]);
+      L[11] = m2l_fma(D[23], m, L[11]);
+      L[12] = m2l_fma(D[25], m, L[12]);
+      L[13] = m2l_fma(D[26], m, L[13]);
+      L[14] = m2l_fma(D[28], m, L[14]);
+      L[15] = m2l_fma(D[29], m, L[15]);
     }
-    { const float m = -__ldg(Mr + 3) * rp;
-      L[0] = fmaf(D[3], m, L[0]);
-      L[1] = fmaf(D[6], m, L[1]);
-      L[2] = fmaf(D[8], m, L[2]);
-      L[3] = fmaf(D[9], m, L[3]);
-      L[4] = fmaf(D[12], m, L[4]);
-      L[5] = fmaf(D[14], m, L[5]);
-      L[6] = fmaf(D[15], m, L[6]);
-      L[7] = fmaf(D[17], m, L[7]);
-      L[8] = fmaf(D[18], m, L[8]);
-      L[9] = fmaf(D[21], m, L[9]);
-      L[10] = fmaf(D[23], m, L[10]);
-      L[11] = fmaf(D[24], m, L[11]);
-      L[12] = fmaf(D[26], m, L[12]);
-      L[13] = fmaf(D[27], m, L[13]);
-      L[14] = fmaf(D[29], m, L[14]);
-      L[15] = fmaf(D[30], m, L[15]);
-    }
-    rp *= rho;
-    { const float m = __ldg(Mr + 4) * rp;
-      L[0] = fmaf(D[4], m, L[0]);
-      L[1] = fmaf(D[10], m, L[1]);
-      L[2] = fmaf(D[11], m, L[2]);
-      L[3] = fmaf(D[12], m, L[3]);
-      L[4] = fmaf(D[19], m, L[4]);
-      L[5] = fmaf(D[20], m, L[5]);
-      L[6] = fmaf(D[21], m, L[6]);
-      L[7] = fmaf(D[22], m, L[7]);
-      L[8] = fmaf(D[23], m, L[8]);
-    }
-    { const float m = __ldg(Mr + 5) * rp;
-      L[0] = fmaf(D[5], m, L[0]);
-      L[1] = fmaf(D[11], m, L[1]);
-      L[2] = fmaf(D[13], m, L[2]);
-      L[3] = fmaf(D[14], m, L[3]);
-      L[4] = fmaf(D[20], m, L[4]);
-      L[5] = fmaf(D[22], m, L[5]);
-      L[6] = fmaf(D[23], m, L[6]);
-      L[7] = fmaf(D[25], m, L[7]);
-      L[8] = fmaf(D[26], m, L[8]);
-    }
-    { const float m = __ldg(Mr + 6) * rp;
-      L[0] = fmaf(D[6], m, L[0]);
-      L[1] = fmaf(D[12], m, L[1]);
-      L[2] = fmaf(D[14], m, L[2]);
-      L[3] = fmaf(D[15], m, L[3]);
-      L[4] = fmaf(D[21], m, L[4]);
-      L[5] = fmaf(D[23], m, L[5]);
-      L[6] = fmaf(D[24], m, L[6]);
-      L[7] = fmaf(D[26], m, L[7]);
-      L[8] = fmaf(D[27], m, L[8]);
-    }
-    { const float m = __ldg(Mr + 7) * rp;
-      L[0] = fmaf(D[7], m, L[0]);
-      L[1] = fmaf(D[13], m, L[1]);
-      L[2] = fmaf(D[16], m, L[2]);
-      L[3] = fmaf(D[17], m, L[3]);
-      L[4] = fmaf(D[22], m, L[4]);
-      L[5] = fmaf(D[25], m, L[5]);
-      L[6] = fmaf(D[26], m, L[6]);
-      L[7] = fmaf(D[28], m, L[7]);
-      L[8] = fmaf(D[29], m, L[8]);
-    }
-    { const float m = __ldg(Mr + 8) * rp;
-      L[0] = fmaf(D[8], m, L[0]);
-      L[1] = fmaf(D[14], m, L[1]);
-      L[2] = fmaf(D[17], m, L[2]);
-      L[3] = fmaf(D[18], m, L[3]);
-      L[4] = fmaf(D[23], m, L[4]);
-      L[5] = fmaf(D[26], m, L[5]);
-      L[6] = fmaf(D[27], m, L[6]);
-      L[7] = fmaf(D[29], m, L[7]);
-      L[8] = fmaf(D[30], m, L[8]);
+    { const T m = -__ldg(Mr + 3) * rp;
+      L[0] = m2l_fma(D[3], m, L[0]);
+      L[1] = m2l_fma(D[6], m, L[1]);
+      L[2] = m2l_fma(D[8], m, L[2]);
+      L[3] = m2l_fma(D[9], m, L[3]);
+      L[4] = m2l_fma(D[12], m, L[4]);
+      L[5] = m2l_fma(D[14], m, L[5]);
+      L[6] = m2l_fma(D[15], m, L[6]);
+      L[7] = m2l_fma(D[17], m, L[7]);
+      L[8] = m2l_fma(D[18], m, L[8]);
+      L[9] = m2l_fma(D[21], m, L[9]);
+      L[10] = m2l_fma(D[23], m, L[10]);
+      L[11] = m2l_fma(D[24], m, L[11]);
+      L[12] = m2l_fma(D[26], m, L[12]);
+      L[13] = m2l_fma(D[27], m, L[13]);
+      L[14] = m2l_fma(D[29], m, L[14]);
+      L[15] = m2l_fma(D[30], m, L[15]);
     }
     rp *= rho;
-    { const float m = -__ldg(Mr + 9) * rp;
-      L[0] = fmaf(D[10], m, L[0]);
-      L[1] = fmaf(D[19], m, L[1]);
-      L[2] = fmaf(D[20], m, L[2]);
-      L[3] = fmaf(D[21], m, L[3]);
+    { const T m = __ldg(Mr + 4) * rp;
+      L[0] = m2l_fma(D[4], m, L[0]);
+      L[1] = m2l_fma(D[10], m, L[1]);
+      L[2] = m2l_fma(D[11], m, L[2]);
+      L[3] = m2l_fma(D[12], m, L[3]);
+      L[4] = m2l_fma(D[19], m, L[4]);
+      L[5] = m2l_fma(D[20], m, L[5]);
+      L[6] = m2l_fma(D[21], m, L[6]);
+      L[7] = m2l_fma(D[22], m, L[7]);
+      L[8] = m2l_fma(D[23], m, L[8]);
     }
-    { const float m = -__ldg(Mr + 10) * rp;
-      L[0] = fmaf(D[11], m, L[0]);
-      L[1] = fmaf(D[20], m, L[1]);
-      L[2] = fmaf(D[22], m, L[2]);
-      L[3] = fmaf(D[23], m, L[3]);
+    { const T m = __ldg(Mr + 5) * rp;
+      L[0] = m2l_fma(D[5], m, L[0]);
+      L[1] = m2l_fma(D[11], m, L[1]);
+      L[2] = m2l_fma(D[13], m, L[2]);
+      L[3] = m2l_fma(D[14], m, L[3]);
+      L[4] = m2l_fma(D[20], m, L[4]);
+      L[5] = m2l_fma(D[22], m, L[5]);
+      L[6] = m2l_fma(D[23], m, L[6]);
+      L[7] = m2l_fma(D[25], m, L[7]);
+      L[8] = m2l_fma(D[26], m, L[8]);
     }
-    { const float m = -__ldg(Mr + 11) * rp;
-      L[0] = fmaf(D[12], m, L[0]);
-      L[1] = fmaf(D[21], m, L[1]);
-      L[2] = fmaf(D[23], m, L[2]);
-      L[3] = fmaf(D[24], m, L[3]);
+    { const T m = __ldg(Mr + 6) * rp;
+      L[0] = m2l_fma(D[6], m, L[0]);
+      L[1] = m2l_fma(D[12], m, L[1]);
+      L[2] = m2l_fma(D[14], m, L[2]);
+      L[3] = m2l_fma(D[15], m, L[3]);
+      L[4] = m2l_fma(D[21], m, L[4]);
+      L[5] = m2l_fma(D[23], m, L[5]);
+      L[6] = m2l_fma(D[24], m, L[6]);
+      L[7] = m2l_fma(D[26], m, L[7]);
+      L[8] = m2l_fma(D[27], m, L[8]);
     }
-    { const float m = -__ldg(Mr + 12) * rp;
-      L[0] = fmaf(D[13], m, L[0]);
-      L[1] = fmaf(D[22], m, L[1]);
-      L[2] = fmaf(D[25], m, L[2]);
-      L[3] = fmaf(D[26], m, L[3]);
+    { const T m = __ldg(Mr + 7) * rp;
+      L[0] = m2l_fma(D[7], m, L[0]);
+      L[1] = m2l_fma(D[13], m, L[1]);
+      L[2] = m2l_fma(D[16], m, L[2]);
+      L[3] = m2l_fma(D[17], m, L[3]);
+      L[4] = m2l_fma(D[22], m, L[4]);
+      L[5] = m2l_fma(D[25], m, L[5]);
+      L[6] = m2l_fma(D[26], m, L[6]);
+      L[7] = m2l_fma(D[28], m, L[7]);
+      L[8] = m2l_fma(D[29], m, L[8]);
     }
-    { const float m = -__ldg(Mr + 13) * rp;
-      L[0] = fmaf(D[14], m, L[0]);
-      L[1] = fmaf(D[23], m, L[1]);
-      L[2] = fmaf(D[26], m, L[2]);
-      L[3] = fmaf(D[27], m, L[3]);
-    }
-    { const float m = -__ldg(Mr + 14) * rp;
-      L[0] = fmaf(D[16], m, L[0]);
-      L[1] = fmaf(D[25], m, L[1]);
-      L[2] = fmaf(D[28], m, L[2]);
-      L[3] = fmaf(D[29], m, L[3]);
-    }
-    { const float m = -__ldg(Mr + 15) * rp;
-      L[0] = fmaf(D[17], m, L[0]);
-      L[1] = fmaf(D[26], m, L[1]);
-      L[2] = fmaf(D[29], m, L[2]);
-      L[3] = fmaf(D[30], m, L[3]);
+    { const T m = __ldg(Mr + 8) * rp;
+      L[0] = m2l_fma(D[8], m, L[0]);
+      L[1] = m2l_fma(D[14], m, L[1]);
+      L[2] = m2l_fma(D[17], m, L[2]);
+      L[3] = m2l_fma(D[18], m, L[3]);
+      L[4] = m2l_fma(D[23], m, L[4]);
+      L[5] = m2l_fma(D[26], m, L[5]);
+      L[6] = m2l_fma(D[27], m, L[6]);
+      L[7] = m2l_fma(D[29], m, L[7]);
+      L[8] = m2l_fma(D[30], m, L[8]);
     }
     rp *= rho;
-    { const float m = __ldg(Mr + 16) * rp;
-      L[0] = fmaf(D[19], m, L[0]);
+    { const T m = -__ldg(Mr + 9) * rp;
+      L[0] = m2l_fma(D[10], m, L[0]);
+      L[1] = m2l_fma(D[19], m, L[1]);
+      L[2] = m2l_fma(D[20], m, L[2]);
+      L[3] = m2l_fma(D[21], m, L[3]);
     }
-    { const float m = __ldg(Mr + 17) * rp;
-      L[0] = fmaf(D[20], m, L[0]);
+    { const T m = -__ldg(Mr + 10) * rp;
+      L[0] = m2l_fma(D[11], m, L[0]);
+      L[1] = m2l_fma(D[20], m, L[1]);
+      L[2] = m2l_fma(D[22], m, L[2]);
+      L[3] = m2l_fma(D[23], m, L[3]);
     }
-    { const float m = __ldg(Mr + 18) * rp;
-      L[0] = fmaf(D[21], m, L[0]);
+    { const T m = -__ldg(Mr + 11) * rp;
+      L[0] = m2l_fma(D[12], m, L[0]);
+      L[1] = m2l_fma(D[21], m, L[1]);
+      L[2] = m2l_fma(D[23], m, L[2]);
+      L[3] = m2l_fma(D[24], m, L[3]);
     }
-    { const float m = __ldg(Mr + 19) * rp;
-      L[0] = fmaf(D[22], m, L[0]);
+    { const T m = -__ldg(Mr + 12) * rp;
+      L[0] = m2l_fma(D[13], m, L[0]);
+      L[1] = m2l_fma(D[22], m, L[1]);
+      L[2] = m2l_fma(D[25], m, L[2]);
+      L[3] = m2l_fma(D[26], m, L[3]);
     }
-    { const float m = __ldg(Mr + 20) * rp;
-      L[0] = fmaf(D[23], m, L[0]);
+    { const T m = -__ldg(Mr + 13) * rp;
+      L[0] = m2l_fma(D[14], m, L[0]);
+      L[1] = m2l_fma(D[23], m, L[1]);
+      L[2] = m2l_fma(D[26], m, L[2]);
+      L[3] = m2l_fma(D[27], m, L[3]);
     }
-    { const float m = __ldg(Mr + 21) * rp;
-      L[0] = fmaf(D[25], m, L[0]);
+    { const T m = -__ldg(Mr + 14) * rp;
+      L[0] = m2l_fma(D[16], m, L[0]);
+      L[1] = m2l_fma(D[25], m, L[1]);
+      L[2] = m2l_fma(D[28], m, L[2]);
+      L[3] = m2l_fma(D[29], m, L[3]);
     }
-    { const float m = __ldg(Mr + 22) * rp;
-      L[0] = fmaf(D[26], m, L[0]);
+    { const T m = -__ldg(Mr + 15) * rp;
+      L[0] = m2l_fma(D[17], m, L[0]);
+      L[1] = m2l_fma(D[26], m, L[1]);
+      L[2] = m2l_fma(D[29], m, L[2]);
+      L[3] = m2l_fma(D[30], m, L[3]);
     }
-    { const float m = __ldg(Mr + 23) * rp;
-      L[0] = fmaf(D[28], m, L[0]);
+    rp *= rho;
+    { const T m = __ldg(Mr + 16) * rp;
+      L[0] = m2l_fma(D[19], m, L[0]);
     }
-    { const float m = __ldg(Mr + 24) * rp;
-      L[0] = fmaf(D[29], m, L[0]);
+    { const T m = __ldg(Mr + 17) * rp;
+      L[0] = m2l_fma(D[20], m, L[0]);
+    }
+    { const T m = __ldg(Mr + 18) * rp;
+      L[0] = m2l_fma(D[21], m, L[0]);
+    }
+    { const T m = __ldg(Mr + 19) * rp;
+      L[0] = m2l_fma(D[22], m, L[0]);
+    }
+    { const T m = __ldg(Mr + 20) * rp;
+      L[0] = m2l_fma(D[23], m, L[0]);
+    }
+    { const T m = __ldg(Mr + 21) * rp;
+      L[0] = m2l_fma(D[25], m, L[0]);
+    }
+    { const T m = __ldg(Mr + 22) * rp;
+      L[0] = m2l_fma(D[26], m, L[0]);
+    }
+    { const T m = __ldg(Mr + 23) * rp;
+      L[0] = m2l_fma(D[28], m, L[0]);
+    }
+    { const T m = __ldg(Mr + 24) * rp;
+      L[0] = m2l_fma(D[29], m, L[0]);
     }
 }
 
-__device__ __forceinline__ void m2l_acc_h_4(const float (&D)[31], const float *__restrict__ Mr, float rho, float (&L)[25])
+template <class T> __device__ __forceinline__ void m2l_acc_h_4(const T (&D)[31], const T *__restrict__ Mr, T rho, T (&L)[25])
 {
-    float rp = 1.0f;
-    { const float m = __ldg(Mr + 0) * rp;
-      L[0] = fmaf(D[0], m, L[0]);
-      L[1] = fmaf(D[1], m, L[1]);
-      L[2] = fmaf(D[2], m, L[2]);
-      L[3] = fmaf(D[3], m, L[3]);
-      L[4] = fmaf(D[4], m, L[4]);
-      L[5] = fmaf(D[5], m, L[5]);
-      L[6] = fmaf(D[6], m, L[6]);
-      L[7] = fmaf(D[7], m, L[7]);
-      L[8] = fmaf(D[8], m, L[8]);
-      L[9] = fmaf(D[10], m, L[9]);
-      L[10] = fmaf(D[11], m, L[10]);
-      L[11] = fmaf(D[12], m, L[11]);
-      L[12] = fmaf(D[13], m, L[12]);
-      L[13] = fmaf(D[14], m, L[13]);
-      L[14] = fmaf(D[16], m, L[14]);
-      L[15] = fmaf(D[17], m, L[15]);
-      L[16] = fmaf(D[19], m, L[16]);
-      L[17] = fmaf(D[20], m, L[17]);
-      L[18] = fmaf(D[21], m, L[18]);
-      L[19] = fmaf(D[22], m, L[19]);
-      L[20] = fmaf(D[23], m, L[20]);
-      L[21] = fmaf(D[25], m, L[21]);
-      L[22] = fmaf(D[26], m, L[22]);
-      L[23] = fmaf(D[28], m, L[23]);
-      L[24] = fmaf(D[29], m, L[24]);
+    T rp = T(1);
+    { const T m = __ldg(Mr + 0) * rp;
+      L[0] = m2l_fma(D[0], m, L[0]);
+      L[1] = m2l_fma(D[1], m, L[1]);
+      L[2] = m2l_fma(D[2], m, L[2]);
+      L[3] = m2l_fma(D[3], m, L[3]);
+      L[4] = m2l_fma(D[4], m, L[4]);
+      L[5] = m2l_fma(D[5], m, L[5]);
+      L[6] = m2l_fma(D[6], m, L[6]);
+      L[7] = m2l_fma(D[7], m, L[7]);
+      L[8] = m2l_fma(D[8], m, L[8]);
+      L[9] = m2l_fma(D[10], m, L[9]);
+      L[10] = m2l_fma(D[11], m, L[10]);
+      L[11] = m2l_fma(D[12], m, L[11]);
+      L[12] = m2l_fma(D[13], m, L[12]);
+      L[13] = m2l_fma(D[14], m, L[13]);
+      L[14] = m2l_fma(D[16], m, L[14]);
+      L[15] = m2l_fma(D[17], m, L[15]);
+      L[16] = m2l_fma(D[19], m, L[16]);
+      L[17] = m2l_fma(D[20], m, L[17]);
+      L[18] = m2l_fma(D[21], m, L[18]);
+      L[19] = m2l_fma(D[22], m, L[19]);
+      L[20] = m2l_fma(D[23], m, L[20]);
+      L[21] = m2l_fma(D[25], m, L[21]);
+      L[22] = m2l_fma(D[26], m, L[22]);
+      L[23] = m2l_fma(D[28], m, L[23]);
+      L[24] = m2l_fma(D[29], m, L[24]);
     }
     rp *= rho;
-    { const float m = -__ldg(Mr + 1) * rp;
-      L[0] = fmaf(D[1], m, L[0]);
-      L[1] = fmaf(D[4], m, L[1]);
-      L[2] = fmaf(D[5], m, L[2]);
-      L[3] = fmaf(D[6], m, L[3]);
-      L[4] = fmaf(D[10], m, L[4]);
-      L[5] = fmaf(D[11], m, L[5]);
-      L[6] = fmaf(D[12], m, L[6]);
-      L[7] = fmaf(D[13], m, L[7]);
-      L[8] = fmaf(D[14], m, L[8]);
-      L[9] = fmaf(D[19], m, L[9]);
-      L[10] = fmaf(D[20], m, L[10]);
-      L[11] = fmaf(D[21], m, L[11]);
-      L[12] = fmaf(D[22], m, L[12]);
-      L[13] = fmaf(D[23], m, L[13]);
-      L[14] = fmaf(D[25], m, L[14]);
-      L[15] = fmaf(D[26], m, L[15]);
+    { const T m = -__ldg(Mr + 1) * rp;
+      L[0] = m2l_fma(D[1], m, L[0]);
+      L[1] = m2l_fma(D[4], m, L[1]);
+      L[2] = m2l_fma(D[5], m, L[2]);
+      L[3] = m2l_fma(D[6], m, L[3]);
+      L[4] = m2l_fma(D[10], m, L[4]);
+      L[5] = m2l_fma(D[11], m, L[5]);
+      L[6] = m2l_fma(D[12], m, L[6]);
+      L[7] = m2l_fma(D[13], m, L[7]);
+      L[8] = m2l_fma(D[14], m, L[8]);
+      L[9] = m2l_fma(D[19], m, L[9]);
+      L[10] = m2l_fma(D[20], m, L[10]);
+      L[11] = m2l_fma(D[21], m, L[11]);
+      L[12] = m2l_fma(D[22], m, L[12]);
+      L[13] = m2l_fma(D[23], m, L[13]);
+      L[14] = m2l_fma(D[25], m, L[14]);
+      L[15] = m2l_fma(D[26], m, L[15]);
     }
-    { const float m = -__ldg(Mr + 2) * rp;
-      L[0] = fmaf(D[2], m, L[0]);
-      L[1] = fmaf(D[5], m, L[1]);
-      L[2] = fmaf(D[7], m, L[2]);
-      L[3] = fmaf(D[8], m, L[3]);
-      L[4] = fmaf(D[11], m, L[4]);
-      L[5] = fmaf(D[13], m, L[5]);
-      L[6] = fmaf(D[14], m, L[6]);
-      L[7] = fmaf(D[16], m, L[7]);
-      L[8] = fmaf(D[17], m, L[8]);
-      L[9] = fmaf(D[20], m, L[9]);
-      L[10] = fmaf(D[22], m, L[10]);
-      L[11] = fmaf(D[23], m, L[11]);
-      L[12] = fmaf(D[25], m, L[12]);
-      L[13] = fmaf(D[26], m, L[13]);
-      L[14] = fmaf(D[28], m, L[14]);
-      L[15] = fmaf(D[29], m, L[15]);
+    { const T m = -__ldg(Mr + 2) * rp;
+      L[0] = m2l_fma(D[2], m, L[0]);
+      L[1] = m2l_fma(D[5], m, L[1]);
+      L[2] = m2l_fma(D[7], m, L[2]);
+      L[3] = m2l_fma(D[8], m, L[3]);
+      L[4] = m2l_fma(D[11], m, L[4]);
+      L[5] = m2l_fma(D[13], m, L[5]);
+      L[6] = m2l_fma(D[14], m, L[6]);
+      L[7] = m2l_fma(D[16], m, L[7]);
+      L[8] = m2l_fma(D[17], m, L[8]);
+      L[9] = m2l_fma(D[20], m, L[9]);
+      L[10] = m2l_fma(D[22], m, L[10]);
+      L[11] = m2l_fma(D[23], m, L[11]);
+      L[12] = m2l_fma(D[25], m, L[12]);
+      L[13] = m2l_fma(D[26], m, L[13]);
+      L[14] = m2l_fma(D[28], m, L[14]);
+      L[15] = m2l_fma(D[29], m, L[15]);
     }
-    { const float m = -__ldg(Mr + 3) * rp;
-      L[0] = fmaf(D[3], m, L[0]);
-      L[1] = fmaf(D[6], m, L[1]);
-      L[2] = fmaf(D[8], m, L[2]);
-      L[3] = fmaf(D[9], m, L[3]);
-      L[4] = fmaf(D[12], m, L[4]);
-      L[5] = fmaf(D[14], m, L[5]);
-      L[6] = fmaf(D[15], m, L[6]);
-      L[7] = fmaf(D[17], m, L[7]);
-      L[8] = fmaf(D[18], m, L[8]);
-      L[9] = fmaf(D[21], m, L[9]);
-      L[10] = fmaf(D[23], m, L[10]);
-      L[11] = fmaf(D[24], m, L[11]);
-      L[12] = fmaf(D[26], m, L[12]);
-      L[13] = fmaf(D[27], m, L[13]);
-      L[14] = fmaf(D[29], m, L[14]);
-      L[15] = fmaf(D[30], m, L[15]);
-    }
-    rp *= rho;
-    { const float m = __ldg(Mr + 4) * rp;
-      L[0] = fmaf(D[4], m, L[0]);
-      L[1] = fmaf(D[10], m, L[1]);
-      L[2] = fmaf(D[11], m, L[2]);
-      L[3] = fmaf(D[12], m, L[3]);
-      L[4] = fmaf(D[19], m, L[4]);
-      L[5] = fmaf(D[20], m, L[5]);
-      L[6] = fmaf(D[21], m, L[6]);
-      L[7] = fmaf(D[22], m, L[7]);
-      L[8] = fmaf(D[23], m, L[8]);
-    }
-    { const float m = __ldg(Mr + 5) * rp;
-      L[0] = fmaf(D[5], m, L[0]);
-      L[1] = fmaf(D[11], m, L[1]);
-      L[2] = fmaf(D[13], m, L[2]);
-      L[3] = fmaf(D[14], m, L[3]);
-      L[4] = fmaf(D[20], m, L[4]);
-      L[5] = fmaf(D[22], m, L[5]);
-      L[6] = fmaf(D[23], m, L[6]);
-      L[7] = fmaf(D[25], m, L[7]);
-      L[8] = fmaf(D[26], m, L[8]);
-    }
-    { const float m = __ldg(Mr + 6) * rp;
-      L[0] = fmaf(D[6], m, L[0]);
-      L[1] = fmaf(D[12], m, L[1]);
-      L[2] = fmaf(D[14], m, L[2]);
-      L[3] = fmaf(D[15], m, L[3]);
-      L[4] = fmaf(D[21], m, L[4]);
-      L[5] = fmaf(D[23], m, L[5]);
-      L[6] = fmaf(D[24], m, L[6]);
-      L[7] = fmaf(D[26], m, L[7]);
-      L[8] = fmaf(D[27], m, L[8]);
-    }
-    { const float m = __ldg(Mr + 7) * rp;
-      L[0] = fmaf(D[7], m, L[0]);
-      L[1] = fmaf(D[13], m, L[1]);
-      L[2] = fmaf(D[16], m, L[2]);
-      L[3] = fmaf(D[17], m, L[3]);
-      L[4] = fmaf(D[22], m, L[4]);
-      L[5] = fmaf(D[25], m, L[5]);
-      L[6] = fmaf(D[26], m, L[6]);
-      L[7] = fmaf(D[28], m, L[7]);
-      L[8] = fmaf(D[29], m, L[8]);
-    }
-    { const float m = __ldg(Mr + 8) * rp;
-      L[0] = fmaf(D[8], m, L[0]);
-      L[1] = fmaf(D[14], m, L[1]);
-      L[2] = fmaf(D[17], m, L[2]);
-      L[3] = fmaf(D[18], m, L[3]);
-      L[4] = fmaf(D[23], m, L[4]);
-      L[5] = fmaf(D[26], m, L[5]);
-      L[6] = fmaf(D[27], m, L[6]);
-      L[7] = fmaf(D[29], m, L[7]);
-      L[8] = fmaf(D[30], m, L[8]);
+    { const T m = -__ldg(Mr + 3) * rp;
+      L[0] = m2l_fma(D[3], m, L[0]);
+      L[1] = m2l_fma(D[6], m, L[1]);
+      L[2] = m2l_fma(D[8], m, L[2]);
+      L[3] = m2l_fma(D[9], m, L[3]);
+      L[4] = m2l_fma(D[12], m, L[4]);
+      L[5] = m2l_fma(D[14], m, L[5]);
+      L[6] = m2l_fma(D[15], m, L[6]);
+      L[7] = m2l_fma(D[17], m, L[7]);
+      L[8] = m2l_fma(D[18], m, L[8]);
+      L[9] = m2l_fma(D[21], m, L[9]);
+      L[10] = m2l_fma(D[23], m, L[10]);
+      L[11] = m2l_fma(D[24], m, L[11]);
+      L[12] = m2l_fma(D[26], m, L[12]);
+      L[13] = m2l_fma(D[27], m, L[13]);
+      L[14] = m2l_fma(D[29], m, L[14]);
+      L[15] = m2l_fma(D[30], m, L[15]);
     }
     rp *= rho;
-    { const float m = -__ldg(Mr + 9) * rp;
-      L[0] = fmaf(D[10], m, L[0]);
-      L[1] = fmaf(D[19], m, L[1]);
-      L[2] = fmaf(D[20], m, L[2]);
-      L[3] = fmaf(D[21], m, L[3]);
+    { const T m = __ldg(Mr + 4) * rp;
+      L[0] = m2l_fma(D[4], m, L[0]);
+      L[1] = m2l_fma(D[10], m, L[1]);
+      L[2] = m2l_fma(D[11], m, L[2]);
+      L[3] = m2l_fma(D[12], m, L[3]);
+      L[4] = m2l_fma(D[19], m, L[4]);
+      L[5] = m2l_fma(D[20], m, L[5]);
+      L[6] = m2l_fma(D[21], m, L[6]);
+      L[7] = m2l_fma(D[22], m, L[7]);
+      L[8] = m2l_fma(D[23], m, L[8]);
     }
-    { const float m = -__ldg(Mr + 10) * rp;
-      L[0] = fmaf(D[11], m, L[0]);
-      L[1] = fmaf(D[20], m, L[1]);
-      L[2] = fmaf(D[22], m, L[2]);
-      L[3] = fmaf(D[23], m, L[3]);
+    { const T m = __ldg(Mr + 5) * rp;
+      L[0] = m2l_fma(D[5], m, L[0]);
+      L[1] = m2l_fma(D[11], m, L[1]);
+      L[2] = m2l_fma(D[13], m, L[2]);
+      L[3] = m2l_fma(D[14], m, L[3]);
+      L[4] = m2l_fma(D[20], m, L[4]);
+      L[5] = m2l_fma(D[22], m, L[5]);
+      L[6] = m2l_fma(D[23], m, L[6]);
+      L[7] = m2l_fma(D[25], m, L[7]);
+      L[8] = m2l_fma(D[26], m, L[8]);
     }
-    { const float m = -__ldg(Mr + 11) * rp;
-      L[0] = fmaf(D[12], m, L[0]);
-      L[1] = fmaf(D[21], m, L[1]);
-      L[2] = fmaf(D[23], m, L[2]);
-      L[3] = fmaf(D[24], m, L[3]);
+    { const T m = __ldg(Mr + 6) * rp;
+      L[0] = m2l_fma(D[6], m, L[0]);
+      L[1] = m2l_fma(D[12], m, L[1]);
+      L[2] = m2l_fma(D[14], m, L[2]);
+      L[3] = m2l_fma(D[15], m, L[3]);
+      L[4] = m2l_fma(D[21], m, L[4]);
+      L[5] = m2l_fma(D[23], m, L[5]);
+      L[6] = m2l_fma(D[24], m, L[6]);
+      L[7] = m2l_fma(D[26], m, L[7]);
+      L[8] = m2l_fma(D[27], m, L[8]);
     }
-    { const float m = -__ldg(Mr + 12) * rp;
-      L[0] = fmaf(D[13], m, L[0]);
-      L[1] = fmaf(D[22], m, L[1]);
-      L[2] = fmaf(D[25], m, L[2]);
-      L[3] = fmaf(D[26], m, L[3]);
+    { const T m = __ldg(Mr + 7) * rp;
+      L[0] = m2l_fma(D[7], m, L[0]);
+      L[1] = m2l_fma(D[13], m, L[1]);
+      L[2] = m2l_fma(D[16], m, L[2]);
+      L[3] = m2l_fma(D[17], m, L[3]);
+      L[4] = m2l_fma(D[22], m, L[4]);
+      L[5] = m2l_fma(D[25], m, L[5]);
+      L[6] = m2l_fma(D[26], m, L[6]);
+      L[7] = m2l_fma(D[28], m, L[7]);
+      L[8] = m2l_fma(D[29], m, L[8]);
     }
-    { const float m = -__ldg(Mr + 13) * rp;
-      L[0] = fmaf(D[14], m, L[0]);
-      L[1] = fmaf(D[23], m, L[1]);
-      L[2] = fmaf(D[26], m, L[2]);
-      L[3] = fmaf(D[27], m, L[3]);
-    }
-    { const float m = -__ldg(Mr + 14) * rp;
-      L[0] = fmaf(D[16], m, L[0]);
-      L[1] = fmaf(D[25], m, L[1]);
-      L[2] = fmaf(D[28], m, L[2]);
-      L[3] = fmaf(D[29], m, L[3]);
-    }
-    { const float m = -__ldg(Mr + 15) * rp;
-      L[0] = fmaf(D[17], m, L[0]);
-      L[1] = fmaf(D[26], m, L[1]);
-      L[2] = fmaf(D[29], m, L[2]);
-      L[3] = fmaf(D[30], m, L[3]);
+    { const T m = __ldg(Mr + 8) * rp;
+      L[0] = m2l_fma(D[8], m, L[0]);
+      L[1] = m2l_fma(D[14], m, L[1]);
+      L[2] = m2l_fma(D[17], m, L[2]);
+      L[3] = m2l_fma(D[18], m, L[3]);
+      L[4] = m2l_fma(D[23], m, L[4]);
+      L[5] = m2l_fma(D[26], m, L[5]);
+      L[6] = m2l_fma(D[27], m, L[6]);
+      L[7] = m2l_fma(D[29], m, L[7]);
+      L[8] = m2l_fma(D[30], m, L[8]);
     }
     rp *= rho;
-    { const float m = __ldg(Mr + 16) * rp;
-      L[0] = fmaf(D[19], m, L[0]);
+    { const T m = -__ldg(Mr + 9) * rp;
+      L[0] = m2l_fma(D[10], m, L[0]);
+      L[1] = m2l_fma(D[19], m, L[1]);
+      L[2] = m2l_fma(D[20], m, L[2]);
+      L[3] = m2l_fma(D[21], m, L[3]);
     }
-    { const float m = __ldg(Mr + 17) * rp;
-      L[0] = fmaf(D[20], m, L[0]);
+    { const T m = -__ldg(Mr + 10) * rp;
+      L[0] = m2l_fma(D[11], m, L[0]);
+      L[1] = m2l_fma(D[20], m, L[1]);
+      L[2] = m2l_fma(D[22], m, L[2]);
+      L[3] = m2l_fma(D[23], m, L[3]);
     }
-    { const float m = __ldg(Mr + 18) * rp;
-      L[0] = fmaf(D[21], m, L[0]);
+    { const T m = -__ldg(Mr + 11) * rp;
+      L[0] = m2l_fma(D[12], m, L[0]);
+      L[1] = m2l_fma(D[21], m, L[1]);
+      L[2] = m2l_fma(D[23], m, L[2]);
+      L[3] = m2l_fma(D[24], m, L[3]);
     }
-    { const float m = __ldg(Mr + 19) * rp;
-      L[0] = fmaf(D[22], m, L[0]);
+    { const T m = -__ldg(Mr + 12) * rp;
+      L[0] = m2l_fma(D[13], m, L[0]);
+      L[1] = m2l_fma(D[22], m, L[1]);
+      L[2] = m2l_fma(D[25], m, L[2]);
+      L[3] = m2l_fma(D[26], m, L[3]);
     }
-    { const float m = __ldg(Mr + 20) * rp;
-      L[0] = fmaf(D[23], m, L[0]);
+    { const T m = -__ldg(Mr + 13) * rp;
+      L[0] = m2l_fma(D[14], m, L[0]);
+      L[1] = m2l_fma(D[23], m, L[1]);
+      L[2] = m2l_fma(D[26], m, L[2]);
+      L[3] = m2l_fma(D[27], m, L[3]);
     }
-    { const float m = __ldg(Mr + 21) * rp;
-      L[0] = fmaf(D[25], m, L[0]);
+    { const T m = -__ldg(Mr + 14) * rp;
+      L[0] = m2l_fma(D[16], m, L[0]);
+      L[1] = m2l_fma(D[25], m, L[1]);
+      L[2] = m2l_fma(D[28], m, L[2]);
+      L[3] = m2l_fma(D[29], m, L[3]);
     }
-    { const float m = __ldg(Mr + 22) * rp;
-      L[0] = fmaf(D[26], m, L[0]);
+    { const T m = -__ldg(Mr + 15) * rp;
+      L[0] = m2l_fma(D[17], m, L[0]);
+      L[1] = m2l_fma(D[26], m, L[1]);
+      L[2] = m2l_fma(D[29], m, L[2]);
+      L[3] = m2l_fma(D[30], m, L[3]);
     }
-    { const float m = __ldg(Mr + 23) * rp;
-      L[0] = fmaf(D[28], m, L[0]);
+    rp *= rho;
+    { const T m = __ldg(Mr + 16) * rp;
+      L[0] = m2l_fma(D[19], m, L[0]);
     }
-    { const float m = __ldg(Mr + 24) * rp;
-      L[0] = fmaf(D[29], m, L[0]);
+    { const T m = __ldg(Mr + 17) * rp;
+      L[0] = m2l_fma(D[20], m, L[0]);
+    }
+    { const T m = __ldg(Mr + 18) * rp;
+      L[0] = m2l_fma(D[21], m, L[0]);
+    }
+    { const T m = __ldg(Mr + 19) * rp;
+      L[0] = m2l_fma(D[22], m, L[0]);
+    }
+    { const T m = __ldg(Mr + 20) * rp;
+      L[0] = m2l_fma(D[23], m, L[0]);
+    }
+    { const T m = __ldg(Mr + 21) * rp;
+      L[0] = m2l_fma(D[25], m, L[0]);
+    }
+    { const T m = __ldg(Mr + 22) * rp;
+      L[0] = m2l_fma(D[26], m, L[0]);
+    }
+    { const T m = __ldg(Mr + 23) * rp;
+      L[0] = m2l_fma(D[28], m, L[0]);
+    }
+    { const T m = __ldg(Mr + 24) * rp;
+      L[0] = m2l_fma(D[29], m, L[0]);
     }
 }
 
-__device__ __forceinline__ void m2l_side_b_h_4(const float (&D)[31], const float *__restrict__ Mr, float (&L)[25])
+template <class T> __device__ __forceinline__ void m2l_side_b_h_4(const T (&D)[31], const T *__restrict__ Mr, T (&L)[25])
 {
-    { const float m = __ldg(Mr + 0);
+    { const T m = __ldg(Mr + 0);
       L[0] = D[0] * m;
       L[1] = -D[1] * m;
       L[2] = -D[2] * m;
@@ -10431,191 +10432,191 @@ __device__ __forceinline__ void m2l_side_b_h_4(const float (&D)[31], const float
       L[23] = D[28] * m;
       L[24] = D[29] * m;
     }
-    { const float m = __ldg(Mr + 1);
-      L[0] = fmaf(D[1], m, L[0]);
-      L[1] = fmaf(-D[4], m, L[1]);
-      L[2] = fmaf(-D[5], m, L[2]);
-      L[3] = fmaf(-D[6], m, L[3]);
-      L[4] = fmaf(D[10], m, L[4]);
-      L[5] = fmaf(D[11], m, L[5]);
-      L[6] = fmaf(D[12], m, L[6]);
-      L[7] = fmaf(D[13], m, L[7]);
-      L[8] = fmaf(D[14], m, L[8]);
-      L[9] = fmaf(-D[19], m, L[9]);
-      L[10] = fmaf(-D[20], m, L[10]);
-      L[11] = fmaf(-D[21], m, L[11]);
-      L[12] = fmaf(-D[22], m, L[12]);
-      L[13] = fmaf(-D[23], m, L[13]);
-      L[14] = fmaf(-D[25], m, L[14]);
-      L[15] = fmaf(-D[26], m, L[15]);
+    { const T m = __ldg(Mr + 1);
+      L[0] = m2l_fma(D[1], m, L[0]);
+      L[1] = m2l_fma(-D[4], m, L[1]);
+      L[2] = m2l_fma(-D[5], m, L[2]);
+      L[3] = m2l_fma(-D[6], m, L[3]);
+      L[4] = m2l_fma(D[10], m, L[4]);
+      L[5] = m2l_fma(D[11], m, L[5]);
+      L[6] = m2l_fma(D[12], m, L[6]);
+      L[7] = m2l_fma(D[13], m, L[7]);
+      L[8] = m2l_fma(D[14], m, L[8]);
+      L[9] = m2l_fma(-D[19], m, L[9]);
+      L[10] = m2l_fma(-D[20], m, L[10]);
+      L[11] = m2l_fma(-D[21], m, L[11]);
+      L[12] = m2l_fma(-D[22], m, L[12]);
+      L[13] = m2l_fma(-D[23], m, L[13]);
+      L[14] = m2l_fma(-D[25], m, L[14]);
+      L[15] = m2l_fma(-D[26], m, L[15]);
     }
-    { const float m = __ldg(Mr + 2);
-      L[0] = fmaf(D[2], m, L[0]);
-      L[1] = fmaf(-D[5], m, L[1]);
-      L[2] = fmaf(-D[7], m, L[2]);
-      L[3] = fmaf(-D[8], m, L[3]);
-      L[4] = fmaf(D[11], m, L[4]);
-      L[5] = fmaf(D[13], m, L[5]);
-      L[6] = fmaf(D[14], m, L[6]);
-      L[7] = fmaf(D[16], m, L[7]);
-      L[8] = fmaf(D[17], m, L[8]);
-      L[9] = fmaf(-D[20], m, L[9]);
-      L[10] = fmaf(-D[22], m, L[10]);
-      L[11] = fmaf(-D[23], m, L[11]);
-      L[12] = fmaf(-D[25], m, L[12]);
-      L[13] = fmaf(-D[26], m, L[13]);
-      L[14] = fmaf(-D[28], m, L[14]);
-      L[15] = fmaf(-D[29], m, L[15]);
+    { const T m = __ldg(Mr + 2);
+      L[0] = m2l_fma(D[2], m, L[0]);
+      L[1] = m2l_fma(-D[5], m, L[1]);
+      L[2] = m2l_fma(-D[7], m, L[2]);
+      L[3] = m2l_fma(-D[8], m, L[3]);
+      L[4] = m2l_fma(D[11], m, L[4]);
+      L[5] = m2l_fma(D[13], m, L[5]);
+      L[6] = m2l_fma(D[14], m, L[6]);
+      L[7] = m2l_fma(D[16], m, L[7]);
+      L[8] = m2l_fma(D[17], m, L[8]);
+      L[9] = m2l_fma(-D[20], m, L[9]);
+      L[10] = m2l_fma(-D[22], m, L[10]);
+      L[11] = m2l_fma(-D[23], m, L[11]);
+      L[12] = m2l_fma(-D[25], m, L[12]);
+      L[13] = m2l_fma(-D[26], m, L[13]);
+      L[14] = m2l_fma(-D[28], m, L[14]);
+      L[15] = m2l_fma(-D[29], m, L[15]);
     }
-    { const float m = __ldg(Mr + 3);
-      L[0] = fmaf(D[3], m, L[0]);
-      L[1] = fmaf(-D[6], m, L[1]);
-      L[2] = fmaf(-D[8], m, L[2]);
-      L[3] = fmaf(-D[9], m, L[3]);
-      L[4] = fmaf(D[12], m, L[4]);
-      L[5] = fmaf(D[14], m, L[5]);
-      L[6] = fmaf(D[15], m, L[6]);
-      L[7] = fmaf(D[17], m, L[7]);
-      L[8] = fmaf(D[18], m, L[8]);
-      L[9] = fmaf(-D[21], m, L[9]);
-      L[10] = fmaf(-D[23], m, L[10]);
-      L[11] = fmaf(-D[24], m, L[11]);
-      L[12] = fmaf(-D[26], m, L[12]);
-      L[13] = fmaf(-D[27], m, L[13]);
-      L[14] = fmaf(-D[29], m, L[14]);
-      L[15] = fmaf(-D[30], m, L[15]);
+    { const T m = __ldg(Mr + 3);
+      L[0] = m2l_fma(D[3], m, L[0]);
+      L[1] = m2l_fma(-D[6], m, L[1]);
+      L[2] = m2l_fma(-D[8], m, L[2]);
+      L[3] = m2l_fma(-D[9], m, L[3]);
+      L[4] = m2l_fma(D[12], m, L[4]);
+      L[5] = m2l_fma(D[14], m, L[5]);
+      L[6] = m2l_fma(D[15], m, L[6]);
+      L[7] = m2l_fma(D[17], m, L[7]);
+      L[8] = m2l_fma(D[18], m, L[8]);
+      L[9] = m2l_fma(-D[21], m, L[9]);
+      L[10] = m2l_fma(-D[23], m, L[10]);
+      L[11] = m2l_fma(-D[24], m, L[11]);
+      L[12] = m2l_fma(-D[26], m, L[12]);
+      L[13] = m2l_fma(-D[27], m, L[13]);
+      L[14] = m2l_fma(-D[29], m, L[14]);
+      L[15] = m2l_fma(-D[30], m, L[15]);
     }
-    { const float m = __ldg(Mr + 4);
-      L[0] = fmaf(D[4], m, L[0]);
-      L[1] = fmaf(-D[10], m, L[1]);
-      L[2] = fmaf(-D[11], m, L[2]);
-      L[3] = fmaf(-D[12], m, L[3]);
-      L[4] = fmaf(D[19], m, L[4]);
-      L[5] = fmaf(D[20], m, L[5]);
-      L[6] = fmaf(D[21], m, L[6]);
-      L[7] = fmaf(D[22], m, L[7]);
-      L[8] = fmaf(D[23], m, L[8]);
+    { const T m = __ldg(Mr + 4);
+      L[0] = m2l_fma(D[4], m, L[0]);
+      L[1] = m2l_fma(-D[10], m, L[1]);
+      L[2] = m2l_fma(-D[11], m, L[2]);
+      L[3] = m2l_fma(-D[12], m, L[3]);
+      L[4] = m2l_fma(D[19], m, L[4]);
+      L[5] = m2l_fma(D[20], m, L[5]);
+      L[6] = m2l_fma(D[21], m, L[6]);
+      L[7] = m2l_fma(D[22], m, L[7]);
+      L[8] = m2l_fma(D[23], m, L[8]);
     }
-    { const float m = __ldg(Mr + 5);
-      L[0] = fmaf(D[5], m, L[0]);
-      L[1] = fmaf(-D[11], m, L[1]);
-      L[2] = fmaf(-D[13], m, L[2]);
-      L[3] = fmaf(-D[14], m, L[3]);
-      L[4] = fmaf(D[20], m, L[4]);
-      L[5] = fmaf(D[22], m, L[5]);
-      L[6] = fmaf(D[23], m, L[6]);
-      L[7] = fmaf(D[25], m, L[7]);
-      L[8] = fmaf(D[26], m, L[8]);
+    { const T m = __ldg(Mr + 5);
+      L[0] = m2l_fma(D[5], m, L[0]);
+      L[1] = m2l_fma(-D[11], m, L[1]);
+      L[2] = m2l_fma(-D[13], m, L[2]);
+      L[3] = m2l_fma(-D[14], m, L[3]);
+      L[4] = m2l_fma(D[20], m, L[4]);
+      L[5] = m2l_fma(D[22], m, L[5]);
+      L[6] = m2l_fma(D[23], m, L[6]);
+      L[7] = m2l_fma(D[25], m, L[7]);
+      L[8] = m2l_fma(D[26], m, L[8]);
     }
-    { const float m = __ldg(Mr + 6);
-      L[0] = fmaf(D[6], m, L[0]);
-      L[1] = fmaf(-D[12], m, L[1]);
-      L[2] = fmaf(-D[14], m, L[2]);
-      L[3] = fmaf(-D[15], m, L[3]);
-      L[4] = fmaf(D[21], m, L[4]);
-      L[5] = fmaf(D[23], m, L[5]);
-      L[6] = fmaf(D[24], m, L[6]);
-      L[7] = fmaf(D[26], m, L[7]);
-      L[8] = fmaf(D[27], m, L[8]);
+    { const T m = __ldg(Mr + 6);
+      L[0] = m2l_fma(D[6], m, L[0]);
+      L[1] = m2l_fma(-D[12], m, L[1]);
+      L[2] = m2l_fma(-D[14], m, L[2]);
+      L[3] = m2l_fma(-D[15], m, L[3]);
+      L[4] = m2l_fma(D[21], m, L[4]);
+      L[5] = m2l_fma(D[23], m, L[5]);
+      L[6] = m2l_fma(D[24], m, L[6]);
+      L[7] = m2l_fma(D[26], m, L[7]);
+      L[8] = m2l_fma(D[27], m, L[8]);
     }
-    { const float m = __ldg(Mr + 7);
-      L[0] = fmaf(D[7], m, L[0]);
-      L[1] = fmaf(-D[13], m, L[1]);
-      L[2] = fmaf(-D[16], m, L[2]);
-      L[3] = fmaf(-D[17], m, L[3]);
-      L[4] = fmaf(D[22], m, L[4]);
-      L[5] = fmaf(D[25], m, L[5]);
-      L[6] = fmaf(D[26], m, L[6]);
-      L[7] = fmaf(D[28], m, L[7]);
-      L[8] = fmaf(D[29], m, L[8]);
+    { const T m = __ldg(Mr + 7);
+      L[0] = m2l_fma(D[7], m, L[0]);
+      L[1] = m2l_fma(-D[13], m, L[1]);
+      L[2] = m2l_fma(-D[16], m, L[2]);
+      L[3] = m2l_fma(-D[17], m, L[3]);
+      L[4] = m2l_fma(D[22], m, L[4]);
+      L[5] = m2l_fma(D[25], m, L[5]);
+      L[6] = m2l_fma(D[26], m, L[6]);
+      L[7] = m2l_fma(D[28], m, L[7]);
+      L[8] = m2l_fma(D[29], m, L[8]);
     }
-    { const float m = __ldg(Mr + 8);
-      L[0] = fmaf(D[8], m, L[0]);
-      L[1] = fmaf(-D[14], m, L[1]);
-      L[2] = fmaf(-D[17], m, L[2]);
-      L[3] = fmaf(-D[18], m, L[3]);
-      L[4] = fmaf(D[23], m, L[4]);
-      L[5] = fmaf(D[26], m, L[5]);
-      L[6] = fmaf(D[27], m, L[6]);
-      L[7] = fmaf(D[29], m, L[7]);
-      L[8] = fmaf(D[30], m, L[8]);
+    { const T m = __ldg(Mr + 8);
+      L[0] = m2l_fma(D[8], m, L[0]);
+      L[1] = m2l_fma(-D[14], m, L[1]);
+      L[2] = m2l_fma(-D[17], m, L[2]);
+      L[3] = m2l_fma(-D[18], m, L[3]);
+      L[4] = m2l_fma(D[23], m, L[4]);
+      L[5] = m2l_fma(D[26], m, L[5]);
+      L[6] = m2l_fma(D[27], m, L[6]);
+      L[7] = m2l_fma(D[29], m, L[7]);
+      L[8] = m2l_fma(D[30], m, L[8]);
     }
-    { const float m = __ldg(Mr + 9);
-      L[0] = fmaf(D[10], m, L[0]);
-      L[1] = fmaf(-D[19], m, L[1]);
-      L[2] = fmaf(-D[20], m, L[2]);
-      L[3] = fmaf(-D[21], m, L[3]);
+    { const T m = __ldg(Mr + 9);
+      L[0] = m2l_fma(D[10], m, L[0]);
+      L[1] = m2l_fma(-D[19], m, L[1]);
+      L[2] = m2l_fma(-D[20], m, L[2]);
+      L[3] = m2l_fma(-D[21], m, L[3]);
     }
-    { const float m = __ldg(Mr + 10);
-      L[0] = fmaf(D[11], m, L[0]);
-      L[1] = fmaf(-D[20], m, L[1]);
-      L[2] = fmaf(-D[22], m, L[2]);
-      L[3] = fmaf(-D[23], m, L[3]);
+    { const T m = __ldg(Mr + 10);
+      L[0] = m2l_fma(D[11], m, L[0]);
+      L[1] = m2l_fma(-D[20], m, L[1]);
+      L[2] = m2l_fma(-D[22], m, L[2]);
+      L[3] = m2l_fma(-D[23], m, L[3]);
     }
-    { const float m = __ldg(Mr + 11);
-      L[0] = fmaf(D[12], m, L[0]);
-      L[1] = fmaf(-D[21], m, L[1]);
-      L[2] = fmaf(-D[23], m, L[2]);
-      L[3] = fmaf(-D[24], m, L[3]);
+    { const T m = __ldg(Mr + 11);
+      L[0] = m2l_fma(D[12], m, L[0]);
+      L[1] = m2l_fma(-D[21], m, L[1]);
+      L[2] = m2l_fma(-D[23], m, L[2]);
+      L[3] = m2l_fma(-D[24], m, L[3]);
     }
-    { const float m = __ldg(Mr + 12);
-      L[0] = fmaf(D[13], m, L[0]);
-      L[1] = fmaf(-D[22], m, L[1]);
-      L[2] = fmaf(-D[25], m, L[2]);
-      L[3] = fmaf(-D[26], m, L[3]);
+    { const T m = __ldg(Mr + 12);
+      L[0] = m2l_fma(D[13], m, L[0]);
+      L[1] = m2l_fma(-D[22], m, L[1]);
+      L[2] = m2l_fma(-D[25], m, L[2]);
+      L[3] = m2l_fma(-D[26], m, L[3]);
     }
-    { const float m = __ldg(Mr + 13);
-      L[0] = fmaf(D[14], m, L[0]);
-      L[1] = fmaf(-D[23], m, L[1]);
-      L[2] = fmaf(-D[26], m, L[2]);
-      L[3] = fmaf(-D[27], m, L[3]);
+    { const T m = __ldg(Mr + 13);
+      L[0] = m2l_fma(D[14], m, L[0]);
+      L[1] = m2l_fma(-D[23], m, L[1]);
+      L[2] = m2l_fma(-D[26], m, L[2]);
+      L[3] = m2l_fma(-D[27], m, L[3]);
     }
-    { const float m = __ldg(Mr + 14);
-      L[0] = fmaf(D[16], m, L[0]);
-      L[1] = fmaf(-D[25], m, L[1]);
-      L[2] = fmaf(-D[28], m, L[2]);
-      L[3] = fmaf(-D[29], m, L[3]);
+    { const T m = __ldg(Mr + 14);
+      L[0] = m2l_fma(D[16], m, L[0]);
+      L[1] = m2l_fma(-D[25], m, L[1]);
+      L[2] = m2l_fma(-D[28], m, L[2]);
+      L[3] = m2l_fma(-D[29], m, L[3]);
     }
-    { const float m = __ldg(Mr + 15);
-      L[0] = fmaf(D[17], m, L[0]);
-      L[1] = fmaf(-D[26], m, L[1]);
-      L[2] = fmaf(-D[29], m, L[2]);
-      L[3] = fmaf(-D[30], m, L[3]);
+    { const T m = __ldg(Mr + 15);
+      L[0] = m2l_fma(D[17], m, L[0]);
+      L[1] = m2l_fma(-D[26], m, L[1]);
+      L[2] = m2l_fma(-D[29], m, L[2]);
+      L[3] = m2l_fma(-D[30], m, L[3]);
     }
-    { const float m = __ldg(Mr + 16);
-      L[0] = fmaf(D[19], m, L[0]);
+    { const T m = __ldg(Mr + 16);
+      L[0] = m2l_fma(D[19], m, L[0]);
     }
-    { const float m = __ldg(Mr + 17);
-      L[0] = fmaf(D[20], m, L[0]);
+    { const T m = __ldg(Mr + 17);
+      L[0] = m2l_fma(D[20], m, L[0]);
     }
-    { const float m = __ldg(Mr + 18);
-      L[0] = fmaf(D[21], m, L[0]);
+    { const T m = __ldg(Mr + 18);
+      L[0] = m2l_fma(D[21], m, L[0]);
     }
-    { const float m = __ldg(Mr + 19);
-      L[0] = fmaf(D[22], m, L[0]);
+    { const T m = __ldg(Mr + 19);
+      L[0] = m2l_fma(D[22], m, L[0]);
     }
-    { const float m = __ldg(Mr + 20);
-      L[0] = fmaf(D[23], m, L[0]);
+    { const T m = __ldg(Mr + 20);
+      L[0] = m2l_fma(D[23], m, L[0]);
     }
-    { const float m = __ldg(Mr + 21);
-      L[0] = fmaf(D[25], m, L[0]);
+    { const T m = __ldg(Mr + 21);
+      L[0] = m2l_fma(D[25], m, L[0]);
     }
-    { const float m = __ldg(Mr + 22);
-      L[0] = fmaf(D[26], m, L[0]);
+    { const T m = __ldg(Mr + 22);
+      L[0] = m2l_fma(D[26], m, L[0]);
     }
-    { const float m = __ldg(Mr + 23);
-      L[0] = fmaf(D[28], m, L[0]);
+    { const T m = __ldg(Mr + 23);
+      L[0] = m2l_fma(D[28], m, L[0]);
     }
-    { const float m = __ldg(Mr + 24);
-      L[0] = fmaf(D[29], m, L[0]);
+    { const T m = __ldg(Mr + 24);
+      L[0] = m2l_fma(D[29], m, L[0]);
     }
 }
 
-__device__ __forceinline__ void m2l_side_a_h_forces_4(const float (&D)[31], const float *__restrict__ Mr, float rho, float (&L)[25])
+template <class T> __device__ __forceinline__ void m2l_side_a_h_forces_4(const T (&D)[31], const T *__restrict__ Mr, T rho, T (&L)[25])
 {
-    L[0] = 0.0f;
-    float rp = 1.0f;
-    { const float m = __ldg(Mr + 0) * rp;
+    L[0] = T(0);
+    T rp = T(1);
+    { const T m = __ldg(Mr + 0) * rp;
       L[1] = D[1] * m;
       L[2] = D[2] * m;
       L[3] = D[3] * m;
@@ -10642,320 +10643,320 @@ __device__ __forceinline__ void m2l_side_a_h_forces_4(const float (&D)[31], cons
       L[24] = D[29] * m;
     }
     rp *= rho;
-    { const float m = -__ldg(Mr + 1) * rp;
-      L[1] = fmaf(D[4], m, L[1]);
-      L[2] = fmaf(D[5], m, L[2]);
-      L[3] = fmaf(D[6], m, L[3]);
-      L[4] = fmaf(D[10], m, L[4]);
-      L[5] = fmaf(D[11], m, L[5]);
-      L[6] = fmaf(D[12], m, L[6]);
-      L[7] = fmaf(D[13], m, L[7]);
-      L[8] = fmaf(D[14], m, L[8]);
-      L[9] = fmaf(D[19], m, L[9]);
-      L[10] = fmaf(D[20], m, L[10]);
-      L[11] = fmaf(D[21], m, L[11]);
-      L[12] = fmaf(D[22], m, L[12]);
-      L[13] = fmaf(D[23], m, L[13]);
-      L[14] = fmaf(D[25], m, L[14]);
-      L[15] = fmaf(D[26], m, L[15]);
+    { const T m = -__ldg(Mr + 1) * rp;
+      L[1] = m2l_fma(D[4], m, L[1]);
+      L[2] = m2l_fma(D[5], m, L[2]);
+      L[3] = m2l_fma(D[6], m, L[3]);
+      L[4] = m2l_fma(D[10], m, L[4]);
+      L[5] = m2l_fma(D[11], m, L[5]);
+      L[6] = m2l_fma(D[12], m, L[6]);
+      L[7] = m2l_fma(D[13], m, L[7]);
+      L[8] = m2l_fma(D[14], m, L[8]);
+      L[9] = m2l_fma(D[19], m, L[9]);
+      L[10] = m2l_fma(D[20], m, L[10]);
+      L[11] = m2l_fma(D[21], m, L[11]);
+      L[12] = m2l_fma(D[22], m, L[12]);
+      L[13] = m2l_fma(D[23], m, L[13]);
+      L[14] = m2l_fma(D[25], m, L[14]);
+      L[15] = m2l_fma(D[26], m, L[15]);
     }
-    { const float m = -__ldg(Mr + 2) * rp;
-      L[1] = fmaf(D[5], m, L[1]);
-      L[2] = fmaf(D[7], m, L[2]);
-      L[3] = fmaf(D[8], m, L[3]);
-      L[4] = fmaf(D[11], m, L[4]);
-      L[5] = fmaf(D[13], m, L[5]);
-      L[6] = fmaf(D[14], m, L[6]);
-      L[7] = fmaf(D[16], m, L[7]);
-      L[8] = fmaf(D[17], m, L[8]);
-      L[9] = fmaf(D[20], m, L[9]);
-      L[10] = fmaf(D[22], m, L[10]);
-      L[11] = fmaf(D[23], m, L[11]);
-      L[12] = fmaf(D[25], m, L[12]);
-      L[13] = fmaf(D[26], m, L[13]);
-      L[14] = fmaf(D[28], m, L[14]);
-      L[15] = fmaf(D[29], m, L[15]);
+    { const T m = -__ldg(Mr + 2) * rp;
+      L[1] = m2l_fma(D[5], m, L[1]);
+      L[2] = m2l_fma(D[7], m, L[2]);
+      L[3] = m2l_fma(D[8], m, L[3]);
+      L[4] = m2l_fma(D[11], m, L[4]);
+      L[5] = m2l_fma(D[13], m, L[5]);
+      L[6] = m2l_fma(D[14], m, L[6]);
+      L[7] = m2l_fma(D[16], m, L[7]);
+      L[8] = m2l_fma(D[17], m, L[8]);
+      L[9] = m2l_fma(D[20], m, L[9]);
+      L[10] = m2l_fma(D[22], m, L[10]);
+      L[11] = m2l_fma(D[23], m, L[11]);
+      L[12] = m2l_fma(D[25], m, L[12]);
+      L[13] = m2l_fma(D[26], m, L[13]);
+      L[14] = m2l_fma(D[28], m, L[14]);
+      L[15] = m2l_fma(D[29], m, L[15]);
     }
-    { const float m = -__ldg(Mr + 3) * rp;
-      L[1] = fmaf(D[6], m, L[1]);
-      L[2] = fmaf(D[8], m, L[2]);
-      L[3] = fmaf(D[9], m, L[3]);
-      L[4] = fmaf(D[12], m, L[4]);
-      L[5] = fmaf(D[14], m, L[5]);
-      L[6] = fmaf(D[15], m, L[6]);
-      L[7] = fmaf(D[17], m, L[7]);
-      L[8] = fmaf(D[18], m, L[8]);
-      L[9] = fmaf(D[21], m, L[9]);
-      L[10] = fmaf(D[23], m, L[10]);
-      L[11] = fmaf(D[24], m, L[11]);
-      L[12] = fmaf(D[26], m, L[12]);
-      L[13] = fmaf(D[27], m, L[13]);
-      L[14] = fmaf(D[29], m, L[14]);
-      L[15] = fmaf(D[30], m, L[15]);
-    }
-    rp *= rho;
-    { const float m = __ldg(Mr + 4) * rp;
-      L[1] = fmaf(D[10], m, L[1]);
-      L[2] = fmaf(D[11], m, L[2]);
-      L[3] = fmaf(D[12], m, L[3]);
-      L[4] = fmaf(D[19], m, L[4]);
-      L[5] = fmaf(D[20], m, L[5]);
-      L[6] = fmaf(D[21], m, L[6]);
-      L[7] = fmaf(D[22], m, L[7]);
-      L[8] = fmaf(D[23], m, L[8]);
-    }
-    { const float m = __ldg(Mr + 5) * rp;
-      L[1] = fmaf(D[11], m, L[1]);
-      L[2] = fmaf(D[13], m, L[2]);
-      L[3] = fmaf(D[14], m, L[3]);
-      L[4] = fmaf(D[20], m, L[4]);
-      L[5] = fmaf(D[22], m, L[5]);
-      L[6] = fmaf(D[23], m, L[6]);
-      L[7] = fmaf(D[25], m, L[7]);
-      L[8] = fmaf(D[26], m, L[8]);
-    }
-    { const float m = __ldg(Mr + 6) * rp;
-      L[1] = fmaf(D[12], m, L[1]);
-      L[2] = fmaf(D[14], m, L[2]);
-      L[3] = fmaf(D[15], m, L[3]);
-      L[4] = fmaf(D[21], m, L[4]);
-      L[5] = fmaf(D[23], m, L[5]);
-      L[6] = fmaf(D[24], m, L[6]);
-      L[7] = fmaf(D[26], m, L[7]);
-      L[8] = fmaf(D[27], m, L[8]);
-    }
-    { const float m = __ldg(Mr + 7) * rp;
-      L[1] = fmaf(D[13], m, L[1]);
-      L[2] = fmaf(D[16], m, L[2]);
-      L[3] = fmaf(D[17], m, L[3]);
-      L[4] = fmaf(D[22], m, L[4]);
-      L[5] = fmaf(D[25], m, L[5]);
-      L[6] = fmaf(D[26], m, L[6]);
-      L[7] = fmaf(D[28], m, L[7]);
-      L[8] = fmaf(D[29], m, L[8]);
-    }
-    { const float m = __ldg(Mr + 8) * rp;
-      L[1] = fmaf(D[14], m, L[1]);
-      L[2] = fmaf(D[17], m, L[2]);
-      L[3] = fmaf(D[18], m, L[3]);
-      L[4] = fmaf(D[23], m, L[4]);
-      L[5] = fmaf(D[26], m, L[5]);
-      L[6] = fmaf(D[27], m, L[6]);
-      L[7] = fmaf(D[29], m, L[7]);
-      L[8] = fmaf(D[30], m, L[8]);
+    { const T m = -__ldg(Mr + 3) * rp;
+      L[1] = m2l_fma(D[6], m, L[1]);
+      L[2] = m2l_fma(D[8], m, L[2]);
+      L[3] = m2l_fma(D[9], m, L[3]);
+      L[4] = m2l_fma(D[12], m, L[4]);
+      L[5] = m2l_fma(D[14], m, L[5]);
+      L[6] = m2l_fma(D[15], m, L[6]);
+      L[7] = m2l_fma(D[17], m, L[7]);
+      L[8] = m2l_fma(D[18], m, L[8]);
+      L[9] = m2l_fma(D[21], m, L[9]);
+      L[10] = m2l_fma(D[23], m, L[10]);
+      L[11] = m2l_fma(D[24], m, L[11]);
+      L[12] = m2l_fma(D[26], m, L[12]);
+      L[13] = m2l_fma(D[27], m, L[13]);
+      L[14] = m2l_fma(D[29], m, L[14]);
+      L[15] = m2l_fma(D[30], m, L[15]);
     }
     rp *= rho;
-    { const float m = -__ldg(Mr + 9) * rp;
-      L[1] = fmaf(D[19], m, L[1]);
-      L[2] = fmaf(D[20], m, L[2]);
-      L[3] = fmaf(D[21], m, L[3]);
+    { const T m = __ldg(Mr + 4) * rp;
+      L[1] = m2l_fma(D[10], m, L[1]);
+      L[2] = m2l_fma(D[11], m, L[2]);
+      L[3] = m2l_fma(D[12], m, L[3]);
+      L[4] = m2l_fma(D[19], m, L[4]);
+      L[5] = m2l_fma(D[20], m, L[5]);
+      L[6] = m2l_fma(D[21], m, L[6]);
+      L[7] = m2l_fma(D[22], m, L[7]);
+      L[8] = m2l_fma(D[23], m, L[8]);
     }
-    { const float m = -__ldg(Mr + 10) * rp;
-      L[1] = fmaf(D[20], m, L[1]);
-      L[2] = fmaf(D[22], m, L[2]);
-      L[3] = fmaf(D[23], m, L[3]);
+    { const T m = __ldg(Mr + 5) * rp;
+      L[1] = m2l_fma(D[11], m, L[1]);
+      L[2] = m2l_fma(D[13], m, L[2]);
+      L[3] = m2l_fma(D[14], m, L[3]);
+      L[4] = m2l_fma(D[20], m, L[4]);
+      L[5] = m2l_fma(D[22], m, L[5]);
+      L[6] = m2l_fma(D[23], m, L[6]);
+      L[7] = m2l_fma(D[25], m, L[7]);
+      L[8] = m2l_fma(D[26], m, L[8]);
     }
-    { const float m = -__ldg(Mr + 11) * rp;
-      L[1] = fmaf(D[21], m, L[1]);
-      L[2] = fmaf(D[23], m, L[2]);
-      L[3] = fmaf(D[24], m, L[3]);
+    { const T m = __ldg(Mr + 6) * rp;
+      L[1] = m2l_fma(D[12], m, L[1]);
+      L[2] = m2l_fma(D[14], m, L[2]);
+      L[3] = m2l_fma(D[15], m, L[3]);
+      L[4] = m2l_fma(D[21], m, L[4]);
+      L[5] = m2l_fma(D[23], m, L[5]);
+      L[6] = m2l_fma(D[24], m, L[6]);
+      L[7] = m2l_fma(D[26], m, L[7]);
+      L[8] = m2l_fma(D[27], m, L[8]);
     }
-    { const float m = -__ldg(Mr + 12) * rp;
-      L[1] = fmaf(D[22], m, L[1]);
-      L[2] = fmaf(D[25], m, L[2]);
-      L[3] = fmaf(D[26], m, L[3]);
+    { const T m = __ldg(Mr + 7) * rp;
+      L[1] = m2l_fma(D[13], m, L[1]);
+      L[2] = m2l_fma(D[16], m, L[2]);
+      L[3] = m2l_fma(D[17], m, L[3]);
+      L[4] = m2l_fma(D[22], m, L[4]);
+      L[5] = m2l_fma(D[25], m, L[5]);
+      L[6] = m2l_fma(D[26], m, L[6]);
+      L[7] = m2l_fma(D[28], m, L[7]);
+      L[8] = m2l_fma(D[29], m, L[8]);
     }
-    { const float m = -__ldg(Mr + 13) * rp;
-      L[1] = fmaf(D[23], m, L[1]);
-      L[2] = fmaf(D[26], m, L[2]);
-      L[3] = fmaf(D[27], m, L[3]);
+    { const T m = __ldg(Mr + 8) * rp;
+      L[1] = m2l_fma(D[14], m, L[1]);
+      L[2] = m2l_fma(D[17], m, L[2]);
+      L[3] = m2l_fma(D[18], m, L[3]);
+      L[4] = m2l_fma(D[23], m, L[4]);
+      L[5] = m2l_fma(D[26], m, L[5]);
+      L[6] = m2l_fma(D[27], m, L[6]);
+      L[7] = m2l_fma(D[29], m, L[7]);
+      L[8] = m2l_fma(D[30], m, L[8]);
     }
-    { const float m = -__ldg(Mr + 14) * rp;
-      L[1] = fmaf(D[25], m, L[1]);
-      L[2] = fmaf(D[28], m, L[2]);
-      L[3] = fmaf(D[29], m, L[3]);
+    rp *= rho;
+    { const T m = -__ldg(Mr + 9) * rp;
+      L[1] = m2l_fma(D[19], m, L[1]);
+      L[2] = m2l_fma(D[20], m, L[2]);
+      L[3] = m2l_fma(D[21], m, L[3]);
     }
-    { const float m = -__ldg(Mr + 15) * rp;
-      L[1] = fmaf(D[26], m, L[1]);
-      L[2] = fmaf(D[29], m, L[2]);
-      L[3] = fmaf(D[30], m, L[3]);
+    { const T m = -__ldg(Mr + 10) * rp;
+      L[1] = m2l_fma(D[20], m, L[1]);
+      L[2] = m2l_fma(D[22], m, L[2]);
+      L[3] = m2l_fma(D[23], m, L[3]);
+    }
+    { const T m = -__ldg(Mr + 11) * rp;
+      L[1] = m2l_fma(D[21], m, L[1]);
+      L[2] = m2l_fma(D[23], m, L[2]);
+      L[3] = m2l_fma(D[24], m, L[3]);
+    }
+    { const T m = -__ldg(Mr + 12) * rp;
+      L[1] = m2l_fma(D[22], m, L[1]);
+      L[2] = m2l_fma(D[25], m, L[2]);
+      L[3] = m2l_fma(D[26], m, L[3]);
+    }
+    { const T m = -__ldg(Mr + 13) * rp;
+      L[1] = m2l_fma(D[23], m, L[1]);
+      L[2] = m2l_fma(D[26], m, L[2]);
+      L[3] = m2l_fma(D[27], m, L[3]);
+    }
+    { const T m = -__ldg(Mr + 14) * rp;
+      L[1] = m2l_fma(D[25], m, L[1]);
+      L[2] = m2l_fma(D[28], m, L[2]);
+      L[3] = m2l_fma(D[29], m, L[3]);
+    }
+    { const T m = -__ldg(Mr + 15) * rp;
+      L[1] = m2l_fma(D[26], m, L[1]);
+      L[2] = m2l_fma(D[29], m, L[2]);
+      L[3] = m2l_fma(D[30], m, L[3]);
     }
 }
 
-__device__ __forceinline__ void m2l_acc_h_forces_4(const float (&D)[31], const float *__restrict__ Mr, float rho, float (&L)[25])
+template <class T> __device__ __forceinline__ void m2l_acc_h_forces_4(const T (&D)[31], const T *__restrict__ Mr, T rho, T (&L)[25])
 {
-    float rp = 1.0f;
-    { const float m = __ldg(Mr + 0) * rp;
-      L[1] = fmaf(D[1], m, L[1]);
-      L[2] = fmaf(D[2], m, L[2]);
-      L[3] = fmaf(D[3], m, L[3]);
-      L[4] = fmaf(D[4], m, L[4]);
-      L[5] = fmaf(D[5], m, L[5]);
-      L[6] = fmaf(D[6], m, L[6]);
-      L[7] = fmaf(D[7], m, L[7]);
-      L[8] = fmaf(D[8], m, L[8]);
-      L[9] = fmaf(D[10], m, L[9]);
-      L[10] = fmaf(D[11], m, L[10]);
-      L[11] = fmaf(D[12], m, L[11]);
-      L[12] = fmaf(D[13], m, L[12]);
-      L[13] = fmaf(D[14], m, L[13]);
-      L[14] = fmaf(D[16], m, L[14]);
-      L[15] = fmaf(D[17], m, L[15]);
-      L[16] = fmaf(D[19], m, L[16]);
-      L[17] = fmaf(D[20], m, L[17]);
-      L[18] = fmaf(D[21], m, L[18]);
-      L[19] = fmaf(D[22], m, L[19]);
-      L[20] = fmaf(D[23], m, L[20]);
-      L[21] = fmaf(D[25], m, L[21]);
-      L[22] = fmaf(D[26], m, L[22]);
-      L[23] = fmaf(D[28], m, L[23]);
-      L[24] = fmaf(D[29], m, L[24]);
+    T rp = T(1);
+    { const T m = __ldg(Mr + 0) * rp;
+      L[1] = m2l_fma(D[1], m, L[1]);
+      L[2] = m2l_fma(D[2], m, L[2]);
+      L[3] = m2l_fma(D[3], m, L[3]);
+      L[4] = m2l_fma(D[4], m, L[4]);
+      L[5] = m2l_fma(D[5], m, L[5]);
+      L[6] = m2l_fma(D[6], m, L[6]);
+      L[7] = m2l_fma(D[7], m, L[7]);
+      L[8] = m2l_fma(D[8], m, L[8]);
+      L[9] = m2l_fma(D[10], m, L[9]);
+      L[10] = m2l_fma(D[11], m, L[10]);
+      L[11] = m2l_fma(D[12], m, L[11]);
+      L[12] = m2l_fma(D[13], m, L[12]);
+      L[13] = m2l_fma(D[14], m, L[13]);
+      L[14] = m2l_fma(D[16], m, L[14]);
+      L[15] = m2l_fma(D[17], m, L[15]);
+      L[16] = m2l_fma(D[19], m, L[16]);
+      L[17] = m2l_fma(D[20], m, L[17]);
+      L[18] = m2l_fma(D[21], m, L[18]);
+      L[19] = m2l_fma(D[22], m, L[19]);
+      L[20] = m2l_fma(D[23], m, L[20]);
+      L[21] = m2l_fma(D[25], m, L[21]);
+      L[22] = m2l_fma(D[26], m, L[22]);
+      L[23] = m2l_fma(D[28], m, L[23]);
+      L[24] = m2l_fma(D[29], m, L[24]);
     }
     rp *= rho;
-    { const float m = -__ldg(Mr + 1) * rp;
-      L[1] = fmaf(D[4], m, L[1]);
-      L[2] = fmaf(D[5], m, L[2]);
-      L[3] = fmaf(D[6], m, L[3]);
-      L[4] = fmaf(D[10], m, L[4]);
-      L[5] = fmaf(D[11], m, L[5]);
-      L[6] = fmaf(D[12], m, L[6]);
-      L[7] = fmaf(D[13], m, L[7]);
-      L[8] = fmaf(D[14], m, L[8]);
-      L[9] = fmaf(D[19], m, L[9]);
-      L[10] = fmaf(D[20], m, L[10]);
-      L[11] = fmaf(D[21], m, L[11]);
-      L[12] = fmaf(D[22], m, L[12]);
-      L[13] = fmaf(D[23], m, L[13]);
-      L[14] = fmaf(D[25], m, L[14]);
-      L[15] = fmaf(D[26], m, L[15]);
+    { const T m = -__ldg(Mr + 1) * rp;
+      L[1] = m2l_fma(D[4], m, L[1]);
+      L[2] = m2l_fma(D[5], m, L[2]);
+      L[3] = m2l_fma(D[6], m, L[3]);
+      L[4] = m2l_fma(D[10], m, L[4]);
+      L[5] = m2l_fma(D[11], m, L[5]);
+      L[6] = m2l_fma(D[12], m, L[6]);
+      L[7] = m2l_fma(D[13], m, L[7]);
+      L[8] = m2l_fma(D[14], m, L[8]);
+      L[9] = m2l_fma(D[19], m, L[9]);
+      L[10] = m2l_fma(D[20], m, L[10]);
+      L[11] = m2l_fma(D[21], m, L[11]);
+      L[12] = m2l_fma(D[22], m, L[12]);
+      L[13] = m2l_fma(D[23], m, L[13]);
+      L[14] = m2l_fma(D[25], m, L[14]);
+      L[15] = m2l_fma(D[26], m, L[15]);
     }
-    { const float m = -__ldg(Mr + 2) * rp;
-      L[1] = fmaf(D[5], m, L[1]);
-      L[2] = fmaf(D[7], m, L[2]);
-      L[3] = fmaf(D[8], m, L[3]);
-      L[4] = fmaf(D[11], m, L[4]);
-      L[5] = fmaf(D[13], m, L[5]);
-      L[6] = fmaf(D[14], m, L[6]);
-      L[7] = fmaf(D[16], m, L[7]);
-      L[8] = fmaf(D[17], m, L[8]);
-      L[9] = fmaf(D[20], m, L[9]);
-      L[10] = fmaf(D[22], m, L[10]);
-      L[11] = fmaf(D[23], m, L[11]);
-      L[12] = fmaf(D[25], m, L[12]);
-      L[13] = fmaf(D[26], m, L[13]);
-      L[14] = fmaf(D[28], m, L[14]);
-      L[15] = fmaf(D[29], m, L[15]);
+    { const T m = -__ldg(Mr + 2) * rp;
+      L[1] = m2l_fma(D[5], m, L[1]);
+      L[2] = m2l_fma(D[7], m, L[2]);
+      L[3] = m2l_fma(D[8], m, L[3]);
+      L[4] = m2l_fma(D[11], m, L[4]);
+      L[5] = m2l_fma(D[13], m, L[5]);
+      L[6] = m2l_fma(D[14], m, L[6]);
+      L[7] = m2l_fma(D[16], m, L[7]);
+      L[8] = m2l_fma(D[17], m, L[8]);
+      L[9] = m2l_fma(D[20], m, L[9]);
+      L[10] = m2l_fma(D[22], m, L[10]);
+      L[11] = m2l_fma(D[23], m, L[11]);
+      L[12] = m2l_fma(D[25], m, L[12]);
+      L[13] = m2l_fma(D[26], m, L[13]);
+      L[14] = m2l_fma(D[28], m, L[14]);
+      L[15] = m2l_fma(D[29], m, L[15]);
     }
-    { const float m = -__ldg(Mr + 3) * rp;
-      L[1] = fmaf(D[6], m, L[1]);
-      L[2] = fmaf(D[8], m, L[2]);
-      L[3] = fmaf(D[9], m, L[3]);
-      L[4] = fmaf(D[12], m, L[4]);
-      L[5] = fmaf(D[14], m, L[5]);
-      L[6] = fmaf(D[15], m, L[6]);
-      L[7] = fmaf(D[17], m, L[7]);
-      L[8] = fmaf(D[18], m, L[8]);
-      L[9] = fmaf(D[21], m, L[9]);
-      L[10] = fmaf(D[23], m, L[10]);
-      L[11] = fmaf(D[24], m, L[11]);
-      L[12] = fmaf(D[26], m, L[12]);
-      L[13] = fmaf(D[27], m, L[13]);
-      L[14] = fmaf(D[29], m, L[14]);
-      L[15] = fmaf(D[30], m, L[15]);
-    }
-    rp *= rho;
-    { const float m = __ldg(Mr + 4) * rp;
-      L[1] = fmaf(D[10], m, L[1]);
-      L[2] = fmaf(D[11], m, L[2]);
-      L[3] = fmaf(D[12], m, L[3]);
-      L[4] = fmaf(D[19], m, L[4]);
-      L[5] = fmaf(D[20], m, L[5]);
-      L[6] = fmaf(D[21], m, L[6]);
-      L[7] = fmaf(D[22], m, L[7]);
-      L[8] = fmaf(D[23], m, L[8]);
-    }
-    { const float m = __ldg(Mr + 5) * rp;
-      L[1] = fmaf(D[11], m, L[1]);
-      L[2] = fmaf(D[13], m, L[2]);
-      L[3] = fmaf(D[14], m, L[3]);
-      L[4] = fmaf(D[20], m, L[4]);
-      L[5] = fmaf(D[22], m, L[5]);
-      L[6] = fmaf(D[23], m, L[6]);
-      L[7] = fmaf(D[25], m, L[7]);
-      L[8] = fmaf(D[26], m, L[8]);
-    }
-    { const float m = __ldg(Mr + 6) * rp;
-      L[1] = fmaf(D[12], m, L[1]);
-      L[2] = fmaf(D[14], m, L[2]);
-      L[3] = fmaf(D[15], m, L[3]);
-      L[4] = fmaf(D[21], m, L[4]);
-      L[5] = fmaf(D[23], m, L[5]);
-      L[6] = fmaf(D[24], m, L[6]);
-      L[7] = fmaf(D[26], m, L[7]);
-      L[8] = fmaf(D[27], m, L[8]);
-    }
-    { const float m = __ldg(Mr + 7) * rp;
-      L[1] = fmaf(D[13], m, L[1]);
-      L[2] = fmaf(D[16], m, L[2]);
-      L[3] = fmaf(D[17], m, L[3]);
-      L[4] = fmaf(D[22], m, L[4]);
-      L[5] = fmaf(D[25], m, L[5]);
-      L[6] = fmaf(D[26], m, L[6]);
-      L[7] = fmaf(D[28], m, L[7]);
-      L[8] = fmaf(D[29], m, L[8]);
-    }
-    { const float m = __ldg(Mr + 8) * rp;
-      L[1] = fmaf(D[14], m, L[1]);
-      L[2] = fmaf(D[17], m, L[2]);
-      L[3] = fmaf(D[18], m, L[3]);
-      L[4] = fmaf(D[23], m, L[4]);
-      L[5] = fmaf(D[26], m, L[5]);
-      L[6] = fmaf(D[27], m, L[6]);
-      L[7] = fmaf(D[29], m, L[7]);
-      L[8] = fmaf(D[30], m, L[8]);
+    { const T m = -__ldg(Mr + 3) * rp;
+      L[1] = m2l_fma(D[6], m, L[1]);
+      L[2] = m2l_fma(D[8], m, L[2]);
+      L[3] = m2l_fma(D[9], m, L[3]);
+      L[4] = m2l_fma(D[12], m, L[4]);
+      L[5] = m2l_fma(D[14], m, L[5]);
+      L[6] = m2l_fma(D[15], m, L[6]);
+      L[7] = m2l_fma(D[17], m, L[7]);
+      L[8] = m2l_fma(D[18], m, L[8]);
+      L[9] = m2l_fma(D[21], m, L[9]);
+      L[10] = m2l_fma(D[23], m, L[10]);
+      L[11] = m2l_fma(D[24], m, L[11]);
+      L[12] = m2l_fma(D[26], m, L[12]);
+      L[13] = m2l_fma(D[27], m, L[13]);
+      L[14] = m2l_fma(D[29], m, L[14]);
+      L[15] = m2l_fma(D[30], m, L[15]);
     }
     rp *= rho;
-    { const float m = -__ldg(Mr + 9) * rp;
-      L[1] = fmaf(D[19], m, L[1]);
-      L[2] = fmaf(D[20], m, L[2]);
-      L[3] = fmaf(D[21], m, L[3]);
+    { const T m = __ldg(Mr + 4) * rp;
+      L[1] = m2l_fma(D[10], m, L[1]);
+      L[2] = m2l_fma(D[11], m, L[2]);
+      L[3] = m2l_fma(D[12], m, L[3]);
+      L[4] = m2l_fma(D[19], m, L[4]);
+      L[5] = m2l_fma(D[20], m, L[5]);
+      L[6] = m2l_fma(D[21], m, L[6]);
+      L[7] = m2l_fma(D[22], m, L[7]);
+      L[8] = m2l_fma(D[23], m, L[8]);
     }
-    { const float m = -__ldg(Mr + 10) * rp;
-      L[1] = fmaf(D[20], m, L[1]);
-      L[2] = fmaf(D[22], m, L[2]);
-      L[3] = fmaf(D[23], m, L[3]);
+    { const T m = __ldg(Mr + 5) * rp;
+      L[1] = m2l_fma(D[11], m, L[1]);
+      L[2] = m2l_fma(D[13], m, L[2]);
+      L[3] = m2l_fma(D[14], m, L[3]);
+      L[4] = m2l_fma(D[20], m, L[4]);
+      L[5] = m2l_fma(D[22], m, L[5]);
+      L[6] = m2l_fma(D[23], m, L[6]);
+      L[7] = m2l_fma(D[25], m, L[7]);
+      L[8] = m2l_fma(D[26], m, L[8]);
     }
-    { const float m = -__ldg(Mr + 11) * rp;
-      L[1] = fmaf(D[21], m, L[1]);
-      L[2] = fmaf(D[23], m, L[2]);
-      L[3] = fmaf(D[24], m, L[3]);
+    { const T m = __ldg(Mr + 6) * rp;
+      L[1] = m2l_fma(D[12], m, L[1]);
+      L[2] = m2l_fma(D[14], m, L[2]);
+      L[3] = m2l_fma(D[15], m, L[3]);
+      L[4] = m2l_fma(D[21], m, L[4]);
+      L[5] = m2l_fma(D[23], m, L[5]);
+      L[6] = m2l_fma(D[24], m, L[6]);
+      L[7] = m2l_fma(D[26], m, L[7]);
+      L[8] = m2l_fma(D[27], m, L[8]);
     }
-    { const float m = -__ldg(Mr + 12) * rp;
-      L[1] = fmaf(D[22], m, L[1]);
-      L[2] = fmaf(D[25], m, L[2]);
-      L[3] = fmaf(D[26], m, L[3]);
+    { const T m = __ldg(Mr + 7) * rp;
+      L[1] = m2l_fma(D[13], m, L[1]);
+      L[2] = m2l_fma(D[16], m, L[2]);
+      L[3] = m2l_fma(D[17], m, L[3]);
+      L[4] = m2l_fma(D[22], m, L[4]);
+      L[5] = m2l_fma(D[25], m, L[5]);
+      L[6] = m2l_fma(D[26], m, L[6]);
+      L[7] = m2l_fma(D[28], m, L[7]);
+      L[8] = m2l_fma(D[29], m, L[8]);
     }
-    { const float m = -__ldg(Mr + 13) * rp;
-      L[1] = fmaf(D[23], m, L[1]);
-      L[2] = fmaf(D[26], m, L[2]);
-      L[3] = fmaf(D[27], m, L[3]);
+    { const T m = __ldg(Mr + 8) * rp;
+      L[1] = m2l_fma(D[14], m, L[1]);
+      L[2] = m2l_fma(D[17], m, L[2]);
+      L[3] = m2l_fma(D[18], m, L[3]);
+      L[4] = m2l_fma(D[23], m, L[4]);
+      L[5] = m2l_fma(D[26], m, L[5]);
+      L[6] = m2l_fma(D[27], m, L[6]);
+      L[7] = m2l_fma(D[29], m, L[7]);
+      L[8] = m2l_fma(D[30], m, L[8]);
     }
-    { const float m = -__ldg(Mr + 14) * rp;
-      L[1] = fmaf(D[25], m, L[1]);
-      L[2] = fmaf(D[28], m, L[2]);
-      L[3] = fmaf(D[29], m, L[3]);
+    rp *= rho;
+    { const T m = -__ldg(Mr + 9) * rp;
+      L[1] = m2l_fma(D[19], m, L[1]);
+      L[2] = m2l_fma(D[20], m, L[2]);
+      L[3] = m2l_fma(D[21], m, L[3]);
     }
-    { const float m = -__ldg(Mr + 15) * rp;
-      L[1] = fmaf(D[26], m, L[1]);
-      L[2] = fmaf(D[29], m, L[2]);
-      L[3] = fmaf(D[30], m, L[3]);
+    { const T m = -__ldg(Mr + 10) * rp;
+      L[1] = m2l_fma(D[20], m, L[1]);
+      L[2] = m2l_fma(D[22], m, L[2]);
+      L[3] = m2l_fma(D[23], m, L[3]);
+    }
+    { const T m = -__ldg(Mr + 11) * rp;
+      L[1] = m2l_fma(D[21], m, L[1]);
+      L[2] = m2l_fma(D[23], m, L[2]);
+      L[3] = m2l_fma(D[24], m, L[3]);
+    }
+    { const T m = -__ldg(Mr + 12) * rp;
+      L[1] = m2l_fma(D[22], m, L[1]);
+      L[2] = m2l_fma(D[25], m, L[2]);
+      L[3] = m2l_fma(D[26], m, L[3]);
+    }
+    { const T m = -__ldg(Mr + 13) * rp;
+      L[1] = m2l_fma(D[23], m, L[1]);
+      L[2] = m2l_fma(D[26], m, L[2]);
+      L[3] = m2l_fma(D[27], m, L[3]);
+    }
+    { const T m = -__ldg(Mr + 14) * rp;
+      L[1] = m2l_fma(D[25], m, L[1]);
+      L[2] = m2l_fma(D[28], m, L[2]);
+      L[3] = m2l_fma(D[29], m, L[3]);
+    }
+    { const T m = -__ldg(Mr + 15) * rp;
+      L[1] = m2l_fma(D[26], m, L[1]);
+      L[2] = m2l_fma(D[29], m, L[2]);
+      L[3] = m2l_fma(D[30], m, L[3]);
     }
 }
 
-__device__ __forceinline__ void m2l_side_b_h_forces_4(const float (&D)[31], const float *__restrict__ Mr, float (&L)[25])
+template <class T> __device__ __forceinline__ void m2l_side_b_h_forces_4(const T (&D)[31], const T *__restrict__ Mr, T (&L)[25])
 {
-    L[0] = 0.0f;
-    { const float m = __ldg(Mr + 0);
+    L[0] = T(0);
+    { const T m = __ldg(Mr + 0);
       L[1] = -D[1] * m;
       L[2] = -D[2] * m;
       L[3] = -D[3] * m;
@@ -10981,181 +10982,181 @@ __device__ __forceinline__ void m2l_side_b_h_forces_4(const float (&D)[31], cons
       L[23] = D[28] * m;
       L[24] = D[29] * m;
     }
-    { const float m = __ldg(Mr + 1);
-      L[1] = fmaf(-D[4], m, L[1]);
-      L[2] = fmaf(-D[5], m, L[2]);
-      L[3] = fmaf(-D[6], m, L[3]);
-      L[4] = fmaf(D[10], m, L[4]);
-      L[5] = fmaf(D[11], m, L[5]);
-      L[6] = fmaf(D[12], m, L[6]);
-      L[7] = fmaf(D[13], m, L[7]);
-      L[8] = fmaf(D[14], m, L[8]);
-      L[9] = fmaf(-D[19], m, L[9]);
-      L[10] = fmaf(-D[20], m, L[10]);
-      L[11] = fmaf(-D[21], m, L[11]);
-      L[12] = fmaf(-D[22], m, L[12]);
-      L[13] = fmaf(-D[23], m, L[13]);
-      L[14] = fmaf(-D[25], m, L[14]);
-      L[15] = fmaf(-D[26], m, L[15]);
+    { const T m = __ldg(Mr + 1);
+      L[1] = m2l_fma(-D[4], m, L[1]);
+      L[2] = m2l_fma(-D[5], m, L[2]);
+      L[3] = m2l_fma(-D[6], m, L[3]);
+      L[4] = m2l_fma(D[10], m, L[4]);
+      L[5] = m2l_fma(D[11], m, L[5]);
+      L[6] = m2l_fma(D[12], m, L[6]);
+      L[7] = m2l_fma(D[13], m, L[7]);
+      L[8] = m2l_fma(D[14], m, L[8]);
+      L[9] = m2l_fma(-D[19], m, L[9]);
+      L[10] = m2l_fma(-D[20], m, L[10]);
+      L[11] = m2l_fma(-D[21], m, L[11]);
+      L[12] = m2l_fma(-D[22], m, L[12]);
+      L[13] = m2l_fma(-D[23], m, L[13]);
+      L[14] = m2l_fma(-D[25], m, L[14]);
+      L[15] = m2l_fma(-D[26], m, L[15]);
     }
-    { const float m = __ldg(Mr + 2);
-      L[1] = fmaf(-D[5], m, L[1]);
-      L[2] = fmaf(-D[7], m, L[2]);
-      L[3] = fmaf(-D[8], m, L[3]);
-      L[4] = fmaf(D[11], m, L[4]);
-      L[5] = fmaf(D[13], m, L[5]);
-      L[6] = fmaf(D[14], m, L[6]);
-      L[7] = fmaf(D[16], m, L[7]);
-      L[8] = fmaf(D[17], m, L[8]);
-      L[9] = fmaf(-D[20], m, L[9]);
-      L[10] = fmaf(-D[22], m, L[10]);
-      L[11] = fmaf(-D[23], m, L[11]);
-      L[12] = fmaf(-D[25], m, L[12]);
-      L[13] = fmaf(-D[26], m, L[13]);
-      L[14] = fmaf(-D[28], m, L[14]);
-      L[15] = fmaf(-D[29], m, L[15]);
+    { const T m = __ldg(Mr + 2);
+      L[1] = m2l_fma(-D[5], m, L[1]);
+      L[2] = m2l_fma(-D[7], m, L[2]);
+      L[3] = m2l_fma(-D[8], m, L[3]);
+      L[4] = m2l_fma(D[11], m, L[4]);
+      L[5] = m2l_fma(D[13], m, L[5]);
+      L[6] = m2l_fma(D[14], m, L[6]);
+      L[7] = m2l_fma(D[16], m, L[7]);
+      L[8] = m2l_fma(D[17], m, L[8]);
+      L[9] = m2l_fma(-D[20], m, L[9]);
+      L[10] = m2l_fma(-D[22], m, L[10]);
+      L[11] = m2l_fma(-D[23], m, L[11]);
+      L[12] = m2l_fma(-D[25], m, L[12]);
+      L[13] = m2l_fma(-D[26], m, L[13]);
+      L[14] = m2l_fma(-D[28], m, L[14]);
+      L[15] = m2l_fma(-D[29], m, L[15]);
     }
-    { const float m = __ldg(Mr + 3);
-      L[1] = fmaf(-D[6], m, L[1]);
-      L[2] = fmaf(-D[8], m, L[2]);
-      L[3] = fmaf(-D[9], m, L[3]);
-      L[4] = fmaf(D[12], m, L[4]);
-      L[5] = fmaf(D[14], m, L[5]);
-      L[6] = fmaf(D[15], m, L[6]);
-      L[7] = fmaf(D[17], m, L[7]);
-      L[8] = fmaf(D[18], m, L[8]);
-      L[9] = fmaf(-D[21], m, L[9]);
-      L[10] = fmaf(-D[23], m, L[10]);
-      L[11] = fmaf(-D[24], m, L[11]);
-      L[12] = fmaf(-D[26], m, L[12]);
-      L[13] = fmaf(-D[27], m, L[13]);
-      L[14] = fmaf(-D[29], m, L[14]);
-      L[15] = fmaf(-D[30], m, L[15]);
+    { const T m = __ldg(Mr + 3);
+      L[1] = m2l_fma(-D[6], m, L[1]);
+      L[2] = m2l_fma(-D[8], m, L[2]);
+      L[3] = m2l_fma(-D[9], m, L[3]);
+      L[4] = m2l_fma(D[12], m, L[4]);
+      L[5] = m2l_fma(D[14], m, L[5]);
+      L[6] = m2l_fma(D[15], m, L[6]);
+      L[7] = m2l_fma(D[17], m, L[7]);
+      L[8] = m2l_fma(D[18], m, L[8]);
+      L[9] = m2l_fma(-D[21], m, L[9]);
+      L[10] = m2l_fma(-D[23], m, L[10]);
+      L[11] = m2l_fma(-D[24], m, L[11]);
+      L[12] = m2l_fma(-D[26], m, L[12]);
+      L[13] = m2l_fma(-D[27], m, L[13]);
+      L[14] = m2l_fma(-D[29], m, L[14]);
+      L[15] = m2l_fma(-D[30], m, L[15]);
     }
-    { const float m = __ldg(Mr + 4);
-      L[1] = fmaf(-D[10], m, L[1]);
-      L[2] = fmaf(-D[11], m, L[2]);
-      L[3] = fmaf(-D[12], m, L[3]);
-      L[4] = fmaf(D[19], m, L[4]);
-      L[5] = fmaf(D[20], m, L[5]);
-      L[6] = fmaf(D[21], m, L[6]);
-      L[7] = fmaf(D[22], m, L[7]);
-      L[8] = fmaf(D[23], m, L[8]);
+    { const T m = __ldg(Mr + 4);
+      L[1] = m2l_fma(-D[10], m, L[1]);
+      L[2] = m2l_fma(-D[11], m, L[2]);
+      L[3] = m2l_fma(-D[12], m, L[3]);
+      L[4] = m2l_fma(D[19], m, L[4]);
+      L[5] = m2l_fma(D[20], m, L[5]);
+      L[6] = m2l_fma(D[21], m, L[6]);
+      L[7] = m2l_fma(D[22], m, L[7]);
+      L[8] = m2l_fma(D[23], m, L[8]);
     }
-    { const float m = __ldg(Mr + 5);
-      L[1] = fmaf(-D[11], m, L[1]);
-      L[2] = fmaf(-D[13], m, L[2]);
-      L[3] = fmaf(-D[14], m, L[3]);
-      L[4] = fmaf(D[20], m, L[4]);
-      L[5] = fmaf(D[22], m, L[5]);
-      L[6] = fmaf(D[23], m, L[6]);
-      L[7] = fmaf(D[25], m, L[7]);
-      L[8] = fmaf(D[26], m, L[8]);
+    { const T m = __ldg(Mr + 5);
+      L[1] = m2l_fma(-D[11], m, L[1]);
+      L[2] = m2l_fma(-D[13], m, L[2]);
+      L[3] = m2l_fma(-D[14], m, L[3]);
+      L[4] = m2l_fma(D[20], m, L[4]);
+      L[5] = m2l_fma(D[22], m, L[5]);
+      L[6] = m2l_fma(D[23], m, L[6]);
+      L[7] = m2l_fma(D[25], m, L[7]);
+      L[8] = m2l_fma(D[26], m, L[8]);
     }
-    { const float m = __ldg(Mr + 6);
-      L[1] = fmaf(-D[12], m, L[1]);
-      L[2] = fmaf(-D[14], m, L[2]);
-      L[3] = fmaf(-D[15], m, L[3]);
-      L[4] = fmaf(D[21], m, L[4]);
-      L[5] = fmaf(D[23], m, L[5]);
-      L[6] = fmaf(D[24], m, L[6]);
-      L[7] = fmaf(D[26], m, L[7]);
-      L[8] = fmaf(D[27], m, L[8]);
+    { const T m = __ldg(Mr + 6);
+      L[1] = m2l_fma(-D[12], m, L[1]);
+      L[2] = m2l_fma(-D[14], m, L[2]);
+      L[3] = m2l_fma(-D[15], m, L[3]);
+      L[4] = m2l_fma(D[21], m, L[4]);
+      L[5] = m2l_fma(D[23], m, L[5]);
+      L[6] = m2l_fma(D[24], m, L[6]);
+      L[7] = m2l_fma(D[26], m, L[7]);
+      L[8] = m2l_fma(D[27], m, L[8]);
     }
-    { const float m = __ldg(Mr + 7);
-      L[1] = fmaf(-D[13], m, L[1]);
-      L[2] = fmaf(-D[16], m, L[2]);
-      L[3] = fmaf(-D[17], m, L[3]);
-      L[4] = fmaf(D[22], m, L[4]);
-      L[5] = fmaf(D[25], m, L[5]);
-      L[6] = fmaf(D[26], m, L[6]);
-      L[7] = fmaf(D[28], m, L[7]);
-      L[8] = fmaf(D[29], m, L[8]);
+    { const T m = __ldg(Mr + 7);
+      L[1] = m2l_fma(-D[13], m, L[1]);
+      L[2] = m2l_fma(-D[16], m, L[2]);
+      L[3] = m2l_fma(-D[17], m, L[3]);
+      L[4] = m2l_fma(D[22], m, L[4]);
+      L[5] = m2l_fma(D[25], m, L[5]);
+      L[6] = m2l_fma(D[26], m, L[6]);
+      L[7] = m2l_fma(D[28], m, L[7]);
+      L[8] = m2l_fma(D[29], m, L[8]);
     }
-    { const float m = __ldg(Mr + 8);
-      L[1] = fmaf(-D[14], m, L[1]);
-      L[2] = fmaf(-D[17], m, L[2]);
-      L[3] = fmaf(-D[18], m, L[3]);
-      L[4] = fmaf(D[23], m, L[4]);
-      L[5] = fmaf(D[26], m, L[5]);
-      L[6] = fmaf(D[27], m, L[6]);
-      L[7] = fmaf(D[29], m, L[7]);
-      L[8] = fmaf(D[30], m, L[8]);
+    { const T m = __ldg(Mr + 8);
+      L[1] = m2l_fma(-D[14], m, L[1]);
+      L[2] = m2l_fma(-D[17], m, L[2]);
+      L[3] = m2l_fma(-D[18], m, L[3]);
+      L[4] = m2l_fma(D[23], m, L[4]);
+      L[5] = m2l_fma(D[26], m, L[5]);
+      L[6] = m2l_fma(D[27], m, L[6]);
+      L[7] = m2l_fma(D[29], m, L[7]);
+      L[8] = m2l_fma(D[30], m, L[8]);
     }
-    { const float m = __ldg(Mr + 9);
-      L[1] = fmaf(-D[19], m, L[1]);
-      L[2] = fmaf(-D[20], m, L[2]);
-      L[3] = fmaf(-D[21], m, L[3]);
+    { const T m = __ldg(Mr + 9);
+      L[1] = m2l_fma(-D[19], m, L[1]);
+      L[2] = m2l_fma(-D[20], m, L[2]);
+      L[3] = m2l_fma(-D[21], m, L[3]);
     }
-    { const float m = __ldg(Mr + 10);
-      L[1] = fmaf(-D[20], m, L[1]);
-      L[2] = fmaf(-D[22], m, L[2]);
-      L[3] = fmaf(-D[23], m, L[3]);
+    { const T m = __ldg(Mr + 10);
+      L[1] = m2l_fma(-D[20], m, L[1]);
+      L[2] = m2l_fma(-D[22], m, L[2]);
+      L[3] = m2l_fma(-D[23], m, L[3]);
     }
-    { const float m = __ldg(Mr + 11);
-      L[1] = fmaf(-D[21], m, L[1]);
-      L[2] = fmaf(-D[23], m, L[2]);
-      L[3] = fmaf(-D[24], m, L[3]);
+    { const T m = __ldg(Mr + 11);
+      L[1] = m2l_fma(-D[21], m, L[1]);
+      L[2] = m2l_fma(-D[23], m, L[2]);
+      L[3] = m2l_fma(-D[24], m, L[3]);
     }
-    { const float m = __ldg(Mr + 12);
-      L[1] = fmaf(-D[22], m, L[1]);
-      L[2] = fmaf(-D[25], m, L[2]);
-      L[3] = fmaf(-D[26], m, L[3]);
+    { const T m = __ldg(Mr + 12);
+      L[1] = m2l_fma(-D[22], m, L[1]);
+      L[2] = m2l_fma(-D[25], m, L[2]);
+      L[3] = m2l_fma(-D[26], m, L[3]);
     }
-    { const float m = __ldg(Mr + 13);
-      L[1] = fmaf(-D[23], m, L[1]);
-      L[2] = fmaf(-D[26], m, L[2]);
-      L[3] = fmaf(-D[27], m, L[3]);
+    { const T m = __ldg(Mr + 13);
+      L[1] = m2l_fma(-D[23], m, L[1]);
+      L[2] = m2l_fma(-D[26], m, L[2]);
+      L[3] = m2l_fma(-D[27], m, L[3]);
     }
-    { const float m = __ldg(Mr + 14);
-      L[1] = fmaf(-D[25], m, L[1]);
-      L[2] = fmaf(-D[28], m, L[2]);
-      L[3] = fmaf(-D[29], m, L[3]);
+    { const T m = __ldg(Mr + 14);
+      L[1] = m2l_fma(-D[25], m, L[1]);
+      L[2] = m2l_fma(-D[28], m, L[2]);
+      L[3] = m2l_fma(-D[29], m, L[3]);
     }
-    { const float m = __ldg(Mr + 15);
-      L[1] = fmaf(-D[26], m, L[1]);
-      L[2] = fmaf(-D[29], m, L[2]);
-      L[3] = fmaf(-D[30], m, L[3]);
+    { const T m = __ldg(Mr + 15);
+      L[1] = m2l_fma(-D[26], m, L[1]);
+      L[2] = m2l_fma(-D[29], m, L[2]);
+      L[3] = m2l_fma(-D[30], m, L[3]);
     }
 }
 
-__device__ __forceinline__ void m2l_reduce_moments_h_4(const float *__restrict__ Ms, float *__restrict__ Mr)
+template <class T> __device__ __forceinline__ void m2l_reduce_moments_h_4(const T *__restrict__ Ms, T *__restrict__ Mr)
 {
-    float v0 = Ms[0];
-    float v1 = Ms[1];
-    float v2 = Ms[2];
-    float v3 = Ms[3];
-    float v4 = Ms[4];
-    float v5 = Ms[5];
-    float v6 = Ms[6];
-    float v7 = Ms[7];
-    float v8 = Ms[8];
-    float v9 = Ms[9];
-    float v10 = Ms[10];
-    float v11 = Ms[11];
-    float v12 = Ms[12];
-    float v13 = Ms[13];
-    float v14 = Ms[14];
-    float v15 = Ms[15];
-    float v16 = Ms[16];
-    float v17 = Ms[17];
-    float v18 = Ms[18];
-    float v19 = Ms[19];
-    float v20 = Ms[20];
-    float v21 = Ms[21];
-    float v22 = Ms[22];
-    float v23 = Ms[23];
-    float v24 = Ms[24];
-    float v25 = Ms[25];
-    float v26 = Ms[26];
-    float v27 = Ms[27];
-    float v28 = Ms[28];
-    float v29 = Ms[29];
-    float v30 = Ms[30];
-    float v31 = Ms[31];
-    float v32 = Ms[32];
-    float v33 = Ms[33];
-    float v34 = Ms[34];
+    T v0 = Ms[0];
+    T v1 = Ms[1];
+    T v2 = Ms[2];
+    T v3 = Ms[3];
+    T v4 = Ms[4];
+    T v5 = Ms[5];
+    T v6 = Ms[6];
+    T v7 = Ms[7];
+    T v8 = Ms[8];
+    T v9 = Ms[9];
+    T v10 = Ms[10];
+    T v11 = Ms[11];
+    T v12 = Ms[12];
+    T v13 = Ms[13];
+    T v14 = Ms[14];
+    T v15 = Ms[15];
+    T v16 = Ms[16];
+    T v17 = Ms[17];
+    T v18 = Ms[18];
+    T v19 = Ms[19];
+    T v20 = Ms[20];
+    T v21 = Ms[21];
+    T v22 = Ms[22];
+    T v23 = Ms[23];
+    T v24 = Ms[24];
+    T v25 = Ms[25];
+    T v26 = Ms[26];
+    T v27 = Ms[27];
+    T v28 = Ms[28];
+    T v29 = Ms[29];
+    T v30 = Ms[30];
+    T v31 = Ms[31];
+    T v32 = Ms[32];
+    T v33 = Ms[33];
+    T v34 = Ms[34];
     v25 -= v34;
     v32 -= v34;
     v12 -= v19;
@@ -11203,148 +11204,147 @@ __device__ __forceinline__ void m2l_reduce_moments_h_4(const float *__restrict__
     Mr[24] = v31;
 }
 
-__device__ __forceinline__ void m2l_complete_locals_h_4(const float *__restrict__ Lr, float *__restrict__ L)
+template <class T> __device__ __forceinline__ void m2l_complete_locals_h_4(const T *__restrict__ Lr, T *__restrict__ L)
 {
-    const float v0 = Lr[0];
+    const T v0 = Lr[0];
     L[0] = v0;
-    const float v1 = Lr[1];
+    const T v1 = Lr[1];
     L[1] = v1;
-    const float v2 = Lr[2];
+    const T v2 = Lr[2];
     L[2] = v2;
-    const float v3 = Lr[3];
+    const T v3 = Lr[3];
     L[3] = v3;
-    const float v4 = Lr[4];
+    const T v4 = Lr[4];
     L[4] = v4;
-    const float v5 = Lr[5];
+    const T v5 = Lr[5];
     L[5] = v5;
-    const float v6 = Lr[6];
+    const T v6 = Lr[6];
     L[6] = v6;
-    const float v7 = Lr[7];
+    const T v7 = Lr[7];
     L[7] = v7;
-    const float v8 = Lr[8];
+    const T v8 = Lr[8];
     L[8] = v8;
-    const float v9 = -v4 - v7;
+    const T v9 = -v4 - v7;
     L[9] = v9;
-    const float v10 = Lr[9];
+    const T v10 = Lr[9];
     L[10] = v10;
-    const float v11 = Lr[10];
+    const T v11 = Lr[10];
     L[11] = v11;
-    const float v12 = Lr[11];
+    const T v12 = Lr[11];
     L[12] = v12;
-    const float v13 = Lr[12];
+    const T v13 = Lr[12];
     L[13] = v13;
-    const float v14 = Lr[13];
+    const T v14 = Lr[13];
     L[14] = v14;
-    const float v15 = -v10 - v13;
+    const T v15 = -v10 - v13;
     L[15] = v15;
-    const float v16 = Lr[14];
+    const T v16 = Lr[14];
     L[16] = v16;
-    const float v17 = Lr[15];
+    const T v17 = Lr[15];
     L[17] = v17;
-    const float v18 = -v11 - v16;
+    const T v18 = -v11 - v16;
     L[18] = v18;
-    const float v19 = -v12 - v17;
+    const T v19 = -v12 - v17;
     L[19] = v19;
-    const float v20 = Lr[16];
+    const T v20 = Lr[16];
     L[20] = v20;
-    const float v21 = Lr[17];
+    const T v21 = Lr[17];
     L[21] = v21;
-    const float v22 = Lr[18];
+    const T v22 = Lr[18];
     L[22] = v22;
-    const float v23 = Lr[19];
+    const T v23 = Lr[19];
     L[23] = v23;
-    const float v24 = Lr[20];
+    const T v24 = Lr[20];
     L[24] = v24;
-    const float v25 = -v20 - v23;
+    const T v25 = -v20 - v23;
     L[25] = v25;
-    const float v26 = Lr[21];
+    const T v26 = Lr[21];
     L[26] = v26;
-    const float v27 = Lr[22];
+    const T v27 = Lr[22];
     L[27] = v27;
-    const float v28 = -v21 - v26;
+    const T v28 = -v21 - v26;
     L[28] = v28;
-    const float v29 = -v22 - v27;
+    const T v29 = -v22 - v27;
     L[29] = v29;
-    const float v30 = Lr[23];
+    const T v30 = Lr[23];
     L[30] = v30;
-    const float v31 = Lr[24];
+    const T v31 = Lr[24];
     L[31] = v31;
-    const float v32 = -v23 - v30;
+    const T v32 = -v23 - v30;
     L[32] = v32;
-    const float v33 = -v24 - v31;
+    const T v33 = -v24 - v31;
     L[33] = v33;
-    const float v34 = -v25 - v32;
+    const T v34 = -v25 - v32;
     L[34] = v34;
 }
 
-__device__ __forceinline__ void m2l_dtensor_h_5(float dx, float dy, float dz, float (&D)[46])
+template <class T> __device__ __forceinline__ void m2l_dtensor_h_5(T dx, T dy, T dz, T (&D)[46])
 {
-    const float s2 = fmaf(dx, dx, fmaf(dy, dy, dz * dz));
-    float si = rsqrtf(s2);
-    si = si * fmaf(-0.5f * s2, si * si, 1.5f);   // one Newton step
-    const float si2 = si * si;
-    const float f0 = -si;
-    const float f1 = -1.0f * f0 * si2;
-    const float f2 = -3.0f * f1 * si2;
-    const float f3 = -5.0f * f2 * si2;
-    const float f4 = -7.0f * f3 * si2;
-    const float f5 = -9.0f * f4 * si2;
-    const float r_0_0 = f0;
-    const float r_1_0 = f1;
-    const float r_2_0 = f2;
-    const float r_3_0 = f3;
-    const float r_4_0 = f4;
-    const float r_5_0 = f5;
-    const float r_0_1 = dx * r_1_0;
-    const float r_1_1 = dx * r_2_0;
-    const float r_2_1 = dx * r_3_0;
-    const float r_3_1 = dx * r_4_0;
-    const float r_4_1 = dx * r_5_0;
-    const float r_0_2 = dy * r_1_0;
-    const float r_1_2 = dy * r_2_0;
-    const float r_2_2 = dy * r_3_0;
-    const float r_3_2 = dy * r_4_0;
-    const float r_4_2 = dy * r_5_0;
-    const float r_0_4 = fmaf(1.0f, r_1_0, dx * r_1_1);
-    const float r_1_4 = fmaf(1.0f, r_2_0, dx * r_2_1);
-    const float r_2_4 = fmaf(1.0f, r_3_0, dx * r_3_1);
-    const float r_3_4 = fmaf(1.0f, r_4_0, dx * r_4_1);
-    const float r_0_5 = dx * r_1_2;
-    const float r_1_5 = dx * r_2_2;
-    const float r_2_5 = dx * r_3_2;
-    const float r_3_5 = dx * r_4_2;
-    const float r_0_7 = fmaf(1.0f, r_1_0, dy * r_1_2);
-    const float r_1_7 = fmaf(1.0f, r_2_0, dy * r_2_2);
-    const float r_2_7 = fmaf(1.0f, r_3_0, dy * r_3_2);
-    const float r_3_7 = fmaf(1.0f, r_4_0, dy * r_4_2);
-    const float r_0_10 = fmaf(2.0f, r_1_1, dx * r_1_4);
-    const float r_1_10 = fmaf(2.0f, r_2_1, dx * r_2_4);
-    const float r_2_10 = fmaf(2.0f, r_3_1, dx * r_3_4);
-    const float r_0_11 = fmaf(1.0f, r_1_2, dx * r_1_5);
-    const float r_1_11 = fmaf(1.0f, r_2_2, dx * r_2_5);
-    const float r_2_11 = fmaf(1.0f, r_3_2, dx * r_3_5);
-    const float r_0_13 = dx * r_1_7;
-    const float r_1_13 = dx * r_2_7;
-    const float r_2_13 = dx * r_3_7;
-    const float r_0_16 = fmaf(2.0f, r_1_2, dy * r_1_7);
-    const float r_1_16 = fmaf(2.0f, r_2_2, dy * r_2_7);
-    const float r_2_16 = fmaf(2.0f, r_3_2, dy * r_3_7);
-    const float r_0_20 = fmaf(3.0f, r_1_4, dx * r_1_10);
-    const float r_1_20 = fmaf(3.0f, r_2_4, dx * r_2_10);
-    const float r_0_21 = fmaf(2.0f, r_1_5, dx * r_1_11);
-    const float r_1_21 = fmaf(2.0f, r_2_5, dx * r_2_11);
-    const float r_0_23 = fmaf(1.0f, r_1_7, dx * r_1_13);
-    const float r_1_23 = fmaf(1.0f, r_2_7, dx * r_2_13);
-    const float r_0_26 = dx * r_1_16;
-    const float r_1_26 = dx * r_2_16;
-    const float r_0_30 = fmaf(3.0f, r_1_7, dy * r_1_16);
-    const float r_1_30 = fmaf(3.0f, r_2_7, dy * r_2_16);
-    const float r_0_35 = fmaf(4.0f, r_1_10, dx * r_1_20);
-    const float r_0_36 = fmaf(3.0f, r_1_11, dx * r_1_21);
-    const float r_0_38 = fmaf(2.0f, r_1_13, dx * r_1_23);
-    const float r_0_41 = fmaf(1.0f, r_1_16, dx * r_1_26);
-    const float r_0_45 = dx * r_1_30;
-    const float r_0_50 = fmaf(4.0f, r_1_16, dy * r_1_30);
+    const T s2 = m2l_fma(dx, dx, m2l_fma(dy, dy, dz * dz));
+    const T si = m2l_rsqrt(s2);
+    const T si2 = si * si;
+    const T f0 = -si;
+    const T f1 = T(-1) * f0 * si2;
+    const T f2 = T(-3) * f1 * si2;
+    const T f3 = T(-5) * f2 * si2;
+    const T f4 = T(-7) * f3 * si2;
+    const T f5 = T(-9) * f4 * si2;
+    const T r_0_0 = f0;
+    const T r_1_0 = f1;
+    const T r_2_0 = f2;
+    const T r_3_0 = f3;
+    const T r_4_0 = f4;
+    const T r_5_0 = f5;
+    const T r_0_1 = dx * r_1_0;
+    const T r_1_1 = dx * r_2_0;
+    const T r_2_1 = dx * r_3_0;
+    const T r_3_1 = dx * r_4_0;
+    const T r_4_1 = dx * r_5_0;
+    const T r_0_2 = dy * r_1_0;
+    const T r_1_2 = dy * r_2_0;
+    const T r_2_2 = dy * r_3_0;
+    const T r_3_2 = dy * r_4_0;
+    const T r_4_2 = dy * r_5_0;
+    const T r_0_4 = m2l_fma(T(1), r_1_0, dx * r_1_1);
+    const T r_1_4 = m2l_fma(T(1), r_2_0, dx * r_2_1);
+    const T r_2_4 = m2l_fma(T(1), r_3_0, dx * r_3_1);
+    const T r_3_4 = m2l_fma(T(1), r_4_0, dx * r_4_1);
+    const T r_0_5 = dx * r_1_2;
+    const T r_1_5 = dx * r_2_2;
+    const T r_2_5 = dx * r_3_2;
+    const T r_3_5 = dx * r_4_2;
+    const T r_0_7 = m2l_fma(T(1), r_1_0, dy * r_1_2);
+    const T r_1_7 = m2l_fma(T(1), r_2_0, dy * r_2_2);
+    const T r_2_7 = m2l_fma(T(1), r_3_0, dy * r_3_2);
+    const T r_3_7 = m2l_fma(T(1), r_4_0, dy * r_4_2);
+    const T r_0_10 = m2l_fma(T(2), r_1_1, dx * r_1_4);
+    const T r_1_10 = m2l_fma(T(2), r_2_1, dx * r_2_4);
+    const T r_2_10 = m2l_fma(T(2), r_3_1, dx * r_3_4);
+    const T r_0_11 = m2l_fma(T(1), r_1_2, dx * r_1_5);
+    const T r_1_11 = m2l_fma(T(1), r_2_2, dx * r_2_5);
+    const T r_2_11 = m2l_fma(T(1), r_3_2, dx * r_3_5);
+    const T r_0_13 = dx * r_1_7;
+    const T r_1_13 = dx * r_2_7;
+    const T r_2_13 = dx * r_3_7;
+    const T r_0_16 = m2l_fma(T(2), r_1_2, dy * r_1_7);
+    const T r_1_16 = m2l_fma(T(2), r_2_2, dy * r_2_7);
+    const T r_2_16 = m2l_fma(T(2), r_3_2, dy * r_3_7);
+    const T r_0_20 = m2l_fma(T(3), r_1_4, dx * r_1_10);
+    const T r_1_20 = m2l_fma(T(3), r_2_4, dx * r_2_10);
+    const T r_0_21 = m2l_fma(T(2), r_1_5, dx * r_1_11);
+    const T r_1_21 = m2l_fma(T(2), r_2_5, dx * r_2_11);
+    const T r_0_23 = m2l_fma(T(1), r_1_7, dx * r_1_13);
+    const T r_1_23 = m2l_fma(T(1), r_2_7, dx * r_2_13);
+    const T r_0_26 = dx * r_1_16;
+    const T r_1_26 = dx * r_2_16;
+    const T r_0_30 = m2l_fma(T(3), r_1_7, dy * r_1_16);
+    const T r_1_30 = m2l_fma(T(3), r_2_7, dy * r_2_16);
+    const T r_0_35 = m2l_fma(T(4), r_1_10, dx * r_1_20);
+    const T r_0_36 = m2l_fma(T(3), r_1_11, dx * r_1_21);
+    const T r_0_38 = m2l_fma(T(2), r_1_13, dx * r_1_23);
+    const T r_0_41 = m2l_fma(T(1), r_1_16, dx * r_1_26);
+    const T r_0_45 = dx * r_1_30;
+    const T r_0_50 = m2l_fma(T(4), r_1_16, dy * r_1_30);
     D[0] = r_0_0;
     D[1] = r_0_1;
     D[2] = r_0_2;
@@ -11393,10 +11393,10 @@ __device__ __forceinline__ void m2l_dtensor_h_5(float dx, float dy, float dz, fl
     D[45] = -D[37] - D[43];
 }
 
-__device__ __forceinline__ void m2l_side_a_h_5(const float (&D)[46], const float *__restrict__ Mr, float rho, float (&L)[36])
+template <class T> __device__ __forceinline__ void m2l_side_a_h_5(const T (&D)[46], const T *__restrict__ Mr, T rho, T (&L)[36])
 {
-    float rp = 1.0f;
-    { const float m = __ldg(Mr + 0) * rp;
+    T rp = T(1);
+    { const T m = __ldg(Mr + 0) * rp;
       L[0] = D[0] * m;
       L[1] = D[1] * m;
       L[2] = D[2] * m;
@@ -11435,733 +11435,733 @@ __device__ __forceinline__ void m2l_side_a_h_5(const float (&D)[46], const float
       L[35] = D[44] * m;
     }
     rp *= rho;
-    { const float m = -__ldg(Mr + 1) * rp;
-      L[0] = fmaf(D[1], m, L[0]);
-      L[1] = fmaf(D[4], m, L[1]);
-      L[2] = fmaf(D[5], m, L[2]);
-      L[3] = fmaf(D[6], m, L[3]);
-      L[4] = fmaf(D[10], m, L[4]);
-      L[5] = fmaf(D[11], m, L[5]);
-      L[6] = fmaf(D[12], m, L[6]);
-      L[7] = fmaf(D[13], m, L[7]);
-      L[8] = fmaf(D[14], m, L[8]);
-      L[9] = fmaf(D[19], m, L[9]);
-      L[10] = fmaf(D[20], m, L[10]);
-      L[11] = fmaf(D[21], m, L[11]);
-      L[12] = fmaf(D[22], m, L[12]);
-      L[13] = fmaf(D[23], m, L[13]);
-      L[14] = fmaf(D[25], m, L[14]);
-      L[15] = fmaf(D[26], m, L[15]);
-      L[16] = fmaf(D[31], m, L[16]);
-      L[17] = fmaf(D[32], m, L[17]);
-      L[18] = fmaf(D[33], m, L[18]);
-      L[19] = fmaf(D[34], m, L[19]);
-      L[20] = fmaf(D[35], m, L[20]);
-      L[21] = fmaf(D[37], m, L[21]);
-      L[22] = fmaf(D[38], m, L[22]);
-      L[23] = fmaf(D[40], m, L[23]);
-      L[24] = fmaf(D[41], m, L[24]);
+    { const T m = -__ldg(Mr + 1) * rp;
+      L[0] = m2l_fma(D[1], m, L[0]);
+      L[1] = m2l_fma(D[4], m, L[1]);
+      L[2] = m2l_fma(D[5], m, L[2]);
+      L[3] = m2l_fma(D[6], m, L[3]);
+      L[4] = m2l_fma(D[10], m, L[4]);
+      L[5] = m2l_fma(D[11], m, L[5]);
+      L[6] = m2l_fma(D[12], m, L[6]);
+      L[7] = m2l_fma(D[13], m, L[7]);
+      L[8] = m2l_fma(D[14], m, L[8]);
+      L[9] = m2l_fma(D[19], m, L[9]);
+      L[10] = m2l_fma(D[20], m, L[10]);
+      L[11] = m2l_fma(D[21], m, L[11]);
+      L[12] = m2l_fma(D[22], m, L[12]);
+      L[13] = m2l_fma(D[23], m, L[13]);
+      L[14] = m2l_fma(D[25], m, L[14]);
+      L[15] = m2l_fma(D[26], m, L[15]);
+      L[16] = m2l_fma(D[31], m, L[16]);
+      L[17] = m2l_fma(D[32], m, L[17]);
+      L[18] = m2l_fma(D[33], m, L[18]);
+      L[19] = m2l_fma(D[34], m, L[19]);
+      L[20] = m2l_fma(D[35], m, L[20]);
+      L[21] = m2l_fma(D[37], m, L[21]);
+      L[22] = m2l_fma(D[38], m, L[22]);
+      L[23] = m2l_fma(D[40], m, L[23]);
+      L[24] = m2l_fma(D[41], m, L[24]);
     }
-    { const float m = -__ldg(Mr + 2) * rp;
-      L[0] = fmaf(D[2], m, L[0]);
-      L[1] = fmaf(D[5], m, L[1]);
-      L[2] = fmaf(D[7], m, L[2]);
-      L[3] = fmaf(D[8], m, L[3]);
-      L[4] = fmaf(D[11], m, L[4]);
-      L[5] = fmaf(D[13], m, L[5]);
-      L[6] = fmaf(D[14], m, L[6]);
-      L[7] = fmaf(D[16], m, L[7]);
-      L[8] = fmaf(D[17], m, L[8]);
-      L[9] = fmaf(D[20], m, L[9]);
-      L[10] = fmaf(D[22], m, L[10]);
-      L[11] = fmaf(D[23], m, L[11]);
-      L[12] = fmaf(D[25], m, L[12]);
-      L[13] = fmaf(D[26], m, L[13]);
-      L[14] = fmaf(D[28], m, L[14]);
-      L[15] = fmaf(D[29], m, L[15]);
-      L[16] = fmaf(D[32], m, L[16]);
-      L[17] = fmaf(D[34], m, L[17]);
-      L[18] = fmaf(D[35], m, L[18]);
-      L[19] = fmaf(D[37], m, L[19]);
-      L[20] = fmaf(D[38], m, L[20]);
-      L[21] = fmaf(D[40], m, L[21]);
-      L[22] = fmaf(D[41], m, L[22]);
-      L[23] = fmaf(D[43], m, L[23]);
-      L[24] = fmaf(D[44], m, L[24]);
+    { const T m = -__ldg(Mr + 2) * rp;
+      L[0] = m2l_fma(D[2], m, L[0]);
+      L[1] = m2l_fma(D[5], m, L[1]);
+      L[2] = m2l_fma(D[7], m, L[2]);
+      L[3] = m2l_fma(D[8], m, L[3]);
+      L[4] = m2l_fma(D[11], m, L[4]);
+      L[5] = m2l_fma(D[13], m, L[5]);
+      L[6] = m2l_fma(D[14], m, L[6]);
+      L[7] = m2l_fma(D[16], m, L[7]);
+      L[8] = m2l_fma(D[17], m, L[8]);
+      L[9] = m2l_fma(D[20], m, L[9]);
+      L[10] = m2l_fma(D[22], m, L[10]);
+      L[11] = m2l_fma(D[23], m, L[11]);
+      L[12] = m2l_fma(D[25], m, L[12]);
+      L[13] = m2l_fma(D[26], m, L[13]);
+      L[14] = m2l_fma(D[28], m, L[14]);
+      L[15] = m2l_fma(D[29], m, L[15]);
+      L[16] = m2l_fma(D[32], m, L[16]);
+      L[17] = m2l_fma(D[34], m, L[17]);
+      L[18] = m2l_fma(D[35], m, L[18]);
+      L[19] = m2l_fma(D[37], m, L[19]);
+      L[20] = m2l_fma(D[38], m, L[20]);
+      L[21] = m2l_fma(D[40], m, L[21]);
+      L[22] = m2l_fma(D[41], m, L[22]);
+      L[23] = m2l_fma(D[43], m, L[23]);
+      L[24] = m2l_fma(D[44], m, L[24]);
     }
-    { const float m = -__ldg(Mr + 3) * rp;
-      L[0] = fmaf(D[3], m, L[0]);
-      L[1] = fmaf(D[6], m, L[1]);
-      L[2] = fmaf(D[8], m, L[2]);
-      L[3] = fmaf(D[9], m, L[3]);
-      L[4] = fmaf(D[12], m, L[4]);
-      L[5] = fmaf(D[14], m, L[5]);
-      L[6] = fmaf(D[15], m, L[6]);
-      L[7] = fmaf(D[17], m, L[7]);
-      L[8] = fmaf(D[18], m, L[8]);
-      L[9] = fmaf(D[21], m, L[9]);
-      L[10] = fmaf(D[23], m, L[10]);
-      L[11] = fmaf(D[24], m, L[11]);
-      L[12] = fmaf(D[26], m, L[12]);
-      L[13] = fmaf(D[27], m, L[13]);
-      L[14] = fmaf(D[29], m, L[14]);
-      L[15] = fmaf(D[30], m, L[15]);
-      L[16] = fmaf(D[33], m, L[16]);
-      L[17] = fmaf(D[35], m, L[17]);
-      L[18] = fmaf(D[36], m, L[18]);
-      L[19] = fmaf(D[38], m, L[19]);
-      L[20] = fmaf(D[39], m, L[20]);
-      L[21] = fmaf(D[41], m, L[21]);
-      L[22] = fmaf(D[42], m, L[22]);
-      L[23] = fmaf(D[44], m, L[23]);
-      L[24] = fmaf(D[45], m, L[24]);
-    }
-    rp *= rho;
-    { const float m = __ldg(Mr + 4) * rp;
-      L[0] = fmaf(D[4], m, L[0]);
-      L[1] = fmaf(D[10], m, L[1]);
-      L[2] = fmaf(D[11], m, L[2]);
-      L[3] = fmaf(D[12], m, L[3]);
-      L[4] = fmaf(D[19], m, L[4]);
-      L[5] = fmaf(D[20], m, L[5]);
-      L[6] = fmaf(D[21], m, L[6]);
-      L[7] = fmaf(D[22], m, L[7]);
-      L[8] = fmaf(D[23], m, L[8]);
-      L[9] = fmaf(D[31], m, L[9]);
-      L[10] = fmaf(D[32], m, L[10]);
-      L[11] = fmaf(D[33], m, L[11]);
-      L[12] = fmaf(D[34], m, L[12]);
-      L[13] = fmaf(D[35], m, L[13]);
-      L[14] = fmaf(D[37], m, L[14]);
-      L[15] = fmaf(D[38], m, L[15]);
-    }
-    { const float m = __ldg(Mr + 5) * rp;
-      L[0] = fmaf(D[5], m, L[0]);
-      L[1] = fmaf(D[11], m, L[1]);
-      L[2] = fmaf(D[13], m, L[2]);
-      L[3] = fmaf(D[14], m, L[3]);
-      L[4] = fmaf(D[20], m, L[4]);
-      L[5] = fmaf(D[22], m, L[5]);
-      L[6] = fmaf(D[23], m, L[6]);
-      L[7] = fmaf(D[25], m, L[7]);
-      L[8] = fmaf(D[26], m, L[8]);
-      L[9] = fmaf(D[32], m, L[9]);
-      L[10] = fmaf(D[34], m, L[10]);
-      L[11] = fmaf(D[35], m, L[11]);
-      L[12] = fmaf(D[37], m, L[12]);
-      L[13] = fmaf(D[38], m, L[13]);
-      L[14] = fmaf(D[40], m, L[14]);
-      L[15] = fmaf(D[41], m, L[15]);
-    }
-    { const float m = __ldg(Mr + 6) * rp;
-      L[0] = fmaf(D[6], m, L[0]);
-      L[1] = fmaf(D[12], m, L[1]);
-      L[2] = fmaf(D[14], m, L[2]);
-      L[3] = fmaf(D[15], m, L[3]);
-      L[4] = fmaf(D[21], m, L[4]);
-      L[5] = fmaf(D[23], m, L[5]);
-      L[6] = fmaf(D[24], m, L[6]);
-      L[7] = fmaf(D[26], m, L[7]);
-      L[8] = fmaf(D[27], m, L[8]);
-      L[9] = fmaf(D[33], m, L[9]);
-      L[10] = fmaf(D[35], m, L[10]);
-      L[11] = fmaf(D[36], m, L[11]);
-      L[12] = fmaf(D[38], m, L[12]);
-      L[13] = fmaf(D[39], m, L[13]);
-      L[14] = fmaf(D[41], m, L[14]);
-      L[15] = fmaf(D[42], m, L[15]);
-    }
-    { const float m = __ldg(Mr + 7) * rp;
-      L[0] = fmaf(D[7], m, L[0]);
-      L[1] = fmaf(D[13], m, L[1]);
-      L[2] = fmaf(D[16], m, L[2]);
-      L[3] = fmaf(D[17], m, L[3]);
-      L[4] = fmaf(D[22], m, L[4]);
-      L[5] = fmaf(D[25], m, L[5]);
-      L[6] = fmaf(D[26], m, L[6]);
-      L[7] = fmaf(D[28], m, L[7]);
-      L[8] = fmaf(D[29], m, L[8]);
-      L[9] = fmaf(D[34], m, L[9]);
-      L[10] = fmaf(D[37], m, L[10]);
-      L[11] = fmaf(D[38], m, L[11]);
-      L[12] = fmaf(D[40], m, L[12]);
-      L[13] = fmaf(D[41], m, L[13]);
-      L[14] = fmaf(D[43], m, L[14]);
-      L[15] = fmaf(D[44], m, L[15]);
-    }
-    { const float m = __ldg(Mr + 8) * rp;
-      L[0] = fmaf(D[8], m, L[0]);
-      L[1] = fmaf(D[14], m, L[1]);
-      L[2] = fmaf(D[17], m, L[2]);
-      L[3] = fmaf(D[18], m, L[3]);
-      L[4] = fmaf(D[23], m, L[4]);
-      L[5] = fmaf(D[26], m, L[5]);
-      L[6] = fmaf(D[27], m, L[6]);
-      L[7] = fmaf(D[29], m, L[7]);
-      L[8] = fmaf(D[30], m, L[8]);
-      L[9] = fmaf(D[35], m, L[9]);
-      L[10] = fmaf(D[38], m, L[10]);
-      L[11] = fmaf(D[39], m, L[11]);
-      L[12] = fmaf(D[41], m, L[12]);
-      L[13] = fmaf(D[42], m, L[13]);
-      L[14] = fmaf(D[44], m, L[14]);
-      L[15] = fmaf(D[45], m, L[15]);
+    { const T m = -__ldg(Mr + 3) * rp;
+      L[0] = m2l_fma(D[3], m, L[0]);
+      L[1] = m2l_fma(D[6], m, L[1]);
+      L[2] = m2l_fma(D[8], m, L[2]);
+      L[3] = m2l_fma(D[9], m, L[3]);
+      L[4] = m2l_fma(D[12], m, L[4]);
+      L[5] = m2l_fma(D[14], m, L[5]);
+      L[6] = m2l_fma(D[15], m, L[6]);
+      L[7] = m2l_fma(D[17], m, L[7]);
+      L[8] = m2l_fma(D[18], m, L[8]);
+      L[9] = m2l_fma(D[21], m, L[9]);
+      L[10] = m2l_fma(D[23], m, L[10]);
+      L[11] = m2l_fma(D[24], m, L[11]);
+      L[12] = m2l_fma(D[26], m, L[12]);
+      L[13] = m2l_fma(D[27], m, L[13]);
+      L[14] = m2l_fma(D[29], m, L[14]);
+      L[15] = m2l_fma(D[30], m, L[15]);
+      L[16] = m2l_fma(D[33], m, L[16]);
+      L[17] = m2l_fma(D[35], m, L[17]);
+      L[18] = m2l_fma(D[36], m, L[18]);
+      L[19] = m2l_fma(D[38], m, L[19]);
+      L[20] = m2l_fma(D[39], m, L[20]);
+      L[21] = m2l_fma(D[41], m, L[21]);
+      L[22] = m2l_fma(D[42], m, L[22]);
+      L[23] = m2l_fma(D[44], m, L[23]);
+      L[24] = m2l_fma(D[45], m, L[24]);
     }
     rp *= rho;
-    { const float m = -__ldg(Mr + 9) * rp;
-      L[0] = fmaf(D[10], m, L[0]);
-      L[1] = fmaf(D[19], m, L[1]);
-      L[2] = fmaf(D[20], m, L[2]);
-      L[3] = fmaf(D[21], m, L[3]);
-      L[4] = fmaf(D[31], m, L[4]);
-      L[5] = fmaf(D[32], m, L[5]);
-      L[6] = fmaf(D[33], m, L[6]);
-      L[7] = fmaf(D[34], m, L[7]);
-      L[8] = fmaf(D[35], m, L[8]);
+    { const T m = __ldg(Mr + 4) * rp;
+      L[0] = m2l_fma(D[4], m, L[0]);
+      L[1] = m2l_fma(D[10], m, L[1]);
+      L[2] = m2l_fma(D[11], m, L[2]);
+      L[3] = m2l_fma(D[12], m, L[3]);
+      L[4] = m2l_fma(D[19], m, L[4]);
+      L[5] = m2l_fma(D[20], m, L[5]);
+      L[6] = m2l_fma(D[21], m, L[6]);
+      L[7] = m2l_fma(D[22], m, L[7]);
+      L[8] = m2l_fma(D[23], m, L[8]);
+      L[9] = m2l_fma(D[31], m, L[9]);
+      L[10] = m2l_fma(D[32], m, L[10]);
+      L[11] = m2l_fma(D[33], m, L[11]);
+      L[12] = m2l_fma(D[34], m, L[12]);
+      L[13] = m2l_fma(D[35], m, L[13]);
+      L[14] = m2l_fma(D[37], m, L[14]);
+      L[15] = m2l_fma(D[38], m, L[15]);
     }
-    { const float m = -__ldg(Mr + 10) * rp;
-      L[0] = fmaf(D[11], m, L[0]);
-      L[1] = fmaf(D[20], m, L[1]);
-      L[2] = fmaf(D[22], m, L[2]);
-      L[3] = fmaf(D[23], m, L[3]);
-      L[4] = fmaf(D[32], m, L[4]);
-      L[5] = fmaf(D[34], m, L[5]);
-      L[6] = fmaf(D[35], m, L[6]);
-      L[7] = fmaf(D[37], m, L[7]);
-      L[8] = fmaf(D[38], m, L[8]);
+    { const T m = __ldg(Mr + 5) * rp;
+      L[0] = m2l_fma(D[5], m, L[0]);
+      L[1] = m2l_fma(D[11], m, L[1]);
+      L[2] = m2l_fma(D[13], m, L[2]);
+      L[3] = m2l_fma(D[14], m, L[3]);
+      L[4] = m2l_fma(D[20], m, L[4]);
+      L[5] = m2l_fma(D[22], m, L[5]);
+      L[6] = m2l_fma(D[23], m, L[6]);
+      L[7] = m2l_fma(D[25], m, L[7]);
+      L[8] = m2l_fma(D[26], m, L[8]);
+      L[9] = m2l_fma(D[32], m, L[9]);
+      L[10] = m2l_fma(D[34], m, L[10]);
+      L[11] = m2l_fma(D[35], m, L[11]);
+      L[12] = m2l_fma(D[37], m, L[12]);
+      L[13] = m2l_fma(D[38], m, L[13]);
+      L[14] = m2l_fma(D[40], m, L[14]);
+      L[15] = m2l_fma(D[41], m, L[15]);
     }
-    { const float m = -__ldg(Mr + 11) * rp;
-      L[0] = fmaf(D[12], m, L[0]);
-      L[1] = fmaf(D[21], m, L[1]);
-      L[2] = fmaf(D[23], m, L[2]);
-      L[3] = fmaf(D[24], m, L[3]);
-      L[4] = fmaf(D[33], m, L[4]);
-      L[5] = fmaf(D[35], m, L[5]);
-      L[6] = fmaf(D[36], m, L[6]);
-      L[7] = fmaf(D[38], m, L[7]);
-      L[8] = fmaf(D[39], m, L[8]);
+    { const T m = __ldg(Mr + 6) * rp;
+      L[0] = m2l_fma(D[6], m, L[0]);
+      L[1] = m2l_fma(D[12], m, L[1]);
+      L[2] = m2l_fma(D[14], m, L[2]);
+      L[3] = m2l_fma(D[15], m, L[3]);
+      L[4] = m2l_fma(D[21], m, L[4]);
+      L[5] = m2l_fma(D[23], m, L[5]);
+      L[6] = m2l_fma(D[24], m, L[6]);
+      L[7] = m2l_fma(D[26], m, L[7]);
+      L[8] = m2l_fma(D[27], m, L[8]);
+      L[9] = m2l_fma(D[33], m, L[9]);
+      L[10] = m2l_fma(D[35], m, L[10]);
+      L[11] = m2l_fma(D[36], m, L[11]);
+      L[12] = m2l_fma(D[38], m, L[12]);
+      L[13] = m2l_fma(D[39], m, L[13]);
+      L[14] = m2l_fma(D[41], m, L[14]);
+      L[15] = m2l_fma(D[42], m, L[15]);
     }
-    { const float m = -__ldg(Mr + 12) * rp;
-      L[0] = fmaf(D[13], m, L[0]);
-      L[1] = fmaf(D[22], m, L[1]);
-      L[2] = fmaf(D[25], m, L[2]);
-      L[3] = fmaf(D[26], m, L[3]);
-      L[4] = fmaf(D[34], m, L[4]);
-      L[5] = fmaf(D[37], m, L[5]);
-      L[6] = fmaf(D[38], m, L[6]);
-      L[7] = fmaf(D[40], m, L[7]);
-      L[8] = fmaf(D[41], m, L[8]);
+    { const T m = __ldg(Mr + 7) * rp;
+      L[0] = m2l_fma(D[7], m, L[0]);
+      L[1] = m2l_fma(D[13], m, L[1]);
+      L[2] = m2l_fma(D[16], m, L[2]);
+      L[3] = m2l_fma(D[17], m, L[3]);
+      L[4] = m2l_fma(D[22], m, L[4]);
+      L[5] = m2l_fma(D[25], m, L[5]);
+      L[6] = m2l_fma(D[26], m, L[6]);
+      L[7] = m2l_fma(D[28], m, L[7]);
+      L[8] = m2l_fma(D[29], m, L[8]);
+      L[9] = m2l_fma(D[34], m, L[9]);
+      L[10] = m2l_fma(D[37], m, L[10]);
+      L[11] = m2l_fma(D[38], m, L[11]);
+      L[12] = m2l_fma(D[40], m, L[12]);
+      L[13] = m2l_fma(D[41], m, L[13]);
+      L[14] = m2l_fma(D[43], m, L[14]);
+      L[15] = m2l_fma(D[44], m, L[15]);
     }
-    { const float m = -__ldg(Mr + 13) * rp;
-      L[0] = fmaf(D[14], m, L[0]);
-      L[1] = fmaf(D[23], m, L[1]);
-      L[2] = fmaf(D[26], m, L[2]);
-      L[3] = fmaf(D[27], m, L[3]);
-      L[4] = fmaf(D[35], m, L[4]);
-      L[5] = fmaf(D[38], m, L[5]);
-      L[6] = fmaf(D[39], m, L[6]);
-      L[7] = fmaf(D[41], m, L[7]);
-      L[8] = fmaf(D[42], m, L[8]);
-    }
-    { const float m = -__ldg(Mr + 14) * rp;
-      L[0] = fmaf(D[16], m, L[0]);
-      L[1] = fmaf(D[25], m, L[1]);
-      L[2] = fmaf(D[28], m, L[2]);
-      L[3] = fmaf(D[29], m, L[3]);
-      L[4] = fmaf(D[37], m, L[4]);
-      L[5] = fmaf(D[40], m, L[5]);
-      L[6] = fmaf(D[41], m, L[6]);
-      L[7] = fmaf(D[43], m, L[7]);
-      L[8] = fmaf(D[44], m, L[8]);
-    }
-    { const float m = -__ldg(Mr + 15) * rp;
-      L[0] = fmaf(D[17], m, L[0]);
-      L[1] = fmaf(D[26], m, L[1]);
-      L[2] = fmaf(D[29], m, L[2]);
-      L[3] = fmaf(D[30], m, L[3]);
-      L[4] = fmaf(D[38], m, L[4]);
-      L[5] = fmaf(D[41], m, L[5]);
-      L[6] = fmaf(D[42], m, L[6]);
-      L[7] = fmaf(D[44], m, L[7]);
-      L[8] = fmaf(D[45], m, L[8]);
-    }
-    rp *= rho;
-    { const float m = __ldg(Mr + 16) * rp;
-      L[0] = fmaf(D[19], m, L[0]);
-      L[1] = fmaf(D[31], m, L[1]);
-      L[2] = fmaf(D[32], m, L[2]);
-      L[3] = fmaf(D[33], m, L[3]);
-    }
-    { const float m = __ldg(Mr + 17) * rp;
-      L[0] = fmaf(D[20], m, L[0]);
-      L[1] = fmaf(D[32], m, L[1]);
-      L[2] = fmaf(D[34], m, L[2]);
-      L[3] = fmaf(D[35], m, L[3]);
-    }
-    { const float m = __ldg(Mr + 18) * rp;
-      L[0] = fmaf(D[21], m, L[0]);
-      L[1] = fmaf(D[33], m, L[1]);
-      L[2] = fmaf(D[35], m, L[2]);
-      L[3] = fmaf(D[36], m, L[3]);
-    }
-    { const float m = __ldg(Mr + 19) * rp;
-      L[0] = fmaf(D[22], m, L[0]);
-      L[1] = fmaf(D[34], m, L[1]);
-      L[2] = fmaf(D[37], m, L[2]);
-      L[3] = fmaf(D[38], m, L[3]);
-    }
-    { const float m = __ldg(Mr + 20) * rp;
-      L[0] = fmaf(D[23], m, L[0]);
-      L[1] = fmaf(D[35], m, L[1]);
-      L[2] = fmaf(D[38], m, L[2]);
-      L[3] = fmaf(D[39], m, L[3]);
-    }
-    { const float m = __ldg(Mr + 21) * rp;
-      L[0] = fmaf(D[25], m, L[0]);
-      L[1] = fmaf(D[37], m, L[1]);
-      L[2] = fmaf(D[40], m, L[2]);
-      L[3] = fmaf(D[41], m, L[3]);
-    }
-    { const float m = __ldg(Mr + 22) * rp;
-      L[0] = fmaf(D[26], m, L[0]);
-      L[1] = fmaf(D[38], m, L[1]);
-      L[2] = fmaf(D[41], m, L[2]);
-      L[3] = fmaf(D[42], m, L[3]);
-    }
-    { const float m = __ldg(Mr + 23) * rp;
-      L[0] = fmaf(D[28], m, L[0]);
-      L[1] = fmaf(D[40], m, L[1]);
-      L[2] = fmaf(D[43], m, L[2]);
-      L[3] = fmaf(D[44], m, L[3]);
-    }
-    { const float m = __ldg(Mr + 24) * rp;
-      L[0] = fmaf(D[29], m, L[0]);
-      L[1] = fmaf(D[41], m, L[1]);
-      L[2] = fmaf(D[44], m, L[2]);
-      L[3] = fmaf(D[45], m, L[3]);
+    { const T m = __ldg(Mr + 8) * rp;
+      L[0] = m2l_fma(D[8], m, L[0]);
+      L[1] = m2l_fma(D[14], m, L[1]);
+      L[2] = m2l_fma(D[17], m, L[2]);
+      L[3] = m2l_fma(D[18], m, L[3]);
+      L[4] = m2l_fma(D[23], m, L[4]);
+      L[5] = m2l_fma(D[26], m, L[5]);
+      L[6] = m2l_fma(D[27], m, L[6]);
+      L[7] = m2l_fma(D[29], m, L[7]);
+      L[8] = m2l_fma(D[30], m, L[8]);
+      L[9] = m2l_fma(D[35], m, L[9]);
+      L[10] = m2l_fma(D[38], m, L[10]);
+      L[11] = m2l_fma(D[39], m, L[11]);
+      L[12] = m2l_fma(D[41], m, L[12]);
+      L[13] = m2l_fma(D[42], m, L[13]);
+      L[14] = m2l_fma(D[44], m, L[14]);
+      L[15] = m2l_fma(D[45], m, L[15]);
     }
     rp *= rho;
-    { const float m = -__ldg(Mr + 25) * rp;
-      L[0] = fmaf(D[31], m, L[0]);
+    { const T m = -__ldg(Mr + 9) * rp;
+      L[0] = m2l_fma(D[10], m, L[0]);
+      L[1] = m2l_fma(D[19], m, L[1]);
+      L[2] = m2l_fma(D[20], m, L[2]);
+      L[3] = m2l_fma(D[21], m, L[3]);
+      L[4] = m2l_fma(D[31], m, L[4]);
+      L[5] = m2l_fma(D[32], m, L[5]);
+      L[6] = m2l_fma(D[33], m, L[6]);
+      L[7] = m2l_fma(D[34], m, L[7]);
+      L[8] = m2l_fma(D[35], m, L[8]);
     }
-    { const float m = -__ldg(Mr + 26) * rp;
-      L[0] = fmaf(D[32], m, L[0]);
+    { const T m = -__ldg(Mr + 10) * rp;
+      L[0] = m2l_fma(D[11], m, L[0]);
+      L[1] = m2l_fma(D[20], m, L[1]);
+      L[2] = m2l_fma(D[22], m, L[2]);
+      L[3] = m2l_fma(D[23], m, L[3]);
+      L[4] = m2l_fma(D[32], m, L[4]);
+      L[5] = m2l_fma(D[34], m, L[5]);
+      L[6] = m2l_fma(D[35], m, L[6]);
+      L[7] = m2l_fma(D[37], m, L[7]);
+      L[8] = m2l_fma(D[38], m, L[8]);
     }
-    { const float m = -__ldg(Mr + 27) * rp;
-      L[0] = fmaf(D[33], m, L[0]);
+    { const T m = -__ldg(Mr + 11) * rp;
+      L[0] = m2l_fma(D[12], m, L[0]);
+      L[1] = m2l_fma(D[21], m, L[1]);
+      L[2] = m2l_fma(D[23], m, L[2]);
+      L[3] = m2l_fma(D[24], m, L[3]);
+      L[4] = m2l_fma(D[33], m, L[4]);
+      L[5] = m2l_fma(D[35], m, L[5]);
+      L[6] = m2l_fma(D[36], m, L[6]);
+      L[7] = m2l_fma(D[38], m, L[7]);
+      L[8] = m2l_fma(D[39], m, L[8]);
     }
-    { const float m = -__ldg(Mr + 28) * rp;
-      L[0] = fmaf(D[34], m, L[0]);
+    { const T m = -__ldg(Mr + 12) * rp;
+      L[0] = m2l_fma(D[13], m, L[0]);
+      L[1] = m2l_fma(D[22], m, L[1]);
+      L[2] = m2l_fma(D[25], m, L[2]);
+      L[3] = m2l_fma(D[26], m, L[3]);
+      L[4] = m2l_fma(D[34], m, L[4]);
+      L[5] = m2l_fma(D[37], m, L[5]);
+      L[6] = m2l_fma(D[38], m, L[6]);
+      L[7] = m2l_fma(D[40], m, L[7]);
+      L[8] = m2l_fma(D[41], m, L[8]);
     }
-    { const float m = -__ldg(Mr + 29) * rp;
-      L[0] = fmaf(D[35], m, L[0]);
+    { const T m = -__ldg(Mr + 13) * rp;
+      L[0] = m2l_fma(D[14], m, L[0]);
+      L[1] = m2l_fma(D[23], m, L[1]);
+      L[2] = m2l_fma(D[26], m, L[2]);
+      L[3] = m2l_fma(D[27], m, L[3]);
+      L[4] = m2l_fma(D[35], m, L[4]);
+      L[5] = m2l_fma(D[38], m, L[5]);
+      L[6] = m2l_fma(D[39], m, L[6]);
+      L[7] = m2l_fma(D[41], m, L[7]);
+      L[8] = m2l_fma(D[42], m, L[8]);
     }
-    { const float m = -__ldg(Mr + 30) * rp;
-      L[0] = fmaf(D[37], m, L[0]);
+    { const T m = -__ldg(Mr + 14) * rp;
+      L[0] = m2l_fma(D[16], m, L[0]);
+      L[1] = m2l_fma(D[25], m, L[1]);
+      L[2] = m2l_fma(D[28], m, L[2]);
+      L[3] = m2l_fma(D[29], m, L[3]);
+      L[4] = m2l_fma(D[37], m, L[4]);
+      L[5] = m2l_fma(D[40], m, L[5]);
+      L[6] = m2l_fma(D[41], m, L[6]);
+      L[7] = m2l_fma(D[43], m, L[7]);
+      L[8] = m2l_fma(D[44], m, L[8]);
     }
-    { const float m = -__ldg(Mr + 31) * rp;
-      L[0] = fmaf(D[38], m, L[0]);
+    { const T m = -__ldg(Mr + 15) * rp;
+      L[0] = m2l_fma(D[17], m, L[0]);
+      L[1] = m2l_fma(D[26], m, L[1]);
+      L[2] = m2l_fma(D[29], m, L[2]);
+      L[3] = m2l_fma(D[30], m, L[3]);
+      L[4] = m2l_fma(D[38], m, L[4]);
+      L[5] = m2l_fma(D[41], m, L[5]);
+      L[6] = m2l_fma(D[42], m, L[6]);
+      L[7] = m2l_fma(D[44], m, L[7]);
+      L[8] = m2l_fma(D[45], m, L[8]);
     }
-    { const float m = -__ldg(Mr + 32) * rp;
-      L[0] = fmaf(D[40], m, L[0]);
+    rp *= rho;
+    { const T m = __ldg(Mr + 16) * rp;
+      L[0] = m2l_fma(D[19], m, L[0]);
+      L[1] = m2l_fma(D[31], m, L[1]);
+      L[2] = m2l_fma(D[32], m, L[2]);
+      L[3] = m2l_fma(D[33], m, L[3]);
     }
-    { const float m = -__ldg(Mr + 33) * rp;
-      L[0] = fmaf(D[41], m, L[0]);
+    { const T m = __ldg(Mr + 17) * rp;
+      L[0] = m2l_fma(D[20], m, L[0]);
+      L[1] = m2l_fma(D[32], m, L[1]);
+      L[2] = m2l_fma(D[34], m, L[2]);
+      L[3] = m2l_fma(D[35], m, L[3]);
     }
-    { const float m = -__ldg(Mr + 34) * rp;
-      L[0] = fmaf(D[43], m, L[0]);
+    { const T m = __ldg(Mr + 18) * rp;
+      L[0] = m2l_fma(D[21], m, L[0]);
+      L[1] = m2l_fma(D[33], m, L[1]);
+      L[2] = m2l_fma(D[35], m, L[2]);
+      L[3] = m2l_fma(D[36], m, L[3]);
     }
-    { const float m = -__ldg(Mr + 35) * rp;
-      L[0] = fmaf(D[44], m, L[0]);
+    { const T m = __ldg(Mr + 19) * rp;
+      L[0] = m2l_fma(D[22], m, L[0]);
+      L[1] = m2l_fma(D[34], m, L[1]);
+      L[2] = m2l_fma(D[37], m, L[2]);
+      L[3] = m2l_fma(D[38], m, L[3]);
+    }
+    { const T m = __ldg(Mr + 20) * rp;
+      L[0] = m2l_fma(D[23], m, L[0]);
+      L[1] = m2l_fma(D[35], m, L[1]);
+      L[2] = m2l_fma(D[38], m, L[2]);
+      L[3] = m2l_fma(D[39], m, L[3]);
+    }
+    { const T m = __ldg(Mr + 21) * rp;
+      L[0] = m2l_fma(D[25], m, L[0]);
+      L[1] = m2l_fma(D[37], m, L[1]);
+      L[2] = m2l_fma(D[40], m, L[2]);
+      L[3] = m2l_fma(D[41], m, L[3]);
+    }
+    { const T m = __ldg(Mr + 22) * rp;
+      L[0] = m2l_fma(D[26], m, L[0]);
+      L[1] = m2l_fma(D[38], m, L[1]);
+      L[2] = m2l_fma(D[41], m, L[2]);
+      L[3] = m2l_fma(D[42], m, L[3]);
+    }
+    { const T m = __ldg(Mr + 23) * rp;
+      L[0] = m2l_fma(D[28], m, L[0]);
+      L[1] = m2l_fma(D[40], m, L[1]);
+      L[2] = m2l_fma(D[43], m, L[2]);
+      L[3] = m2l_fma(D[44], m, L[3]);
+    }
+    { const T m = __ldg(Mr + 24) * rp;
+      L[0] = m2l_fma(D[29], m, L[0]);
+      L[1] = m2l_fma(D[41], m, L[1]);
+      L[2] = m2l_fma(D[44], m, L[2]);
+      L[3] = m2l_fma(D[45], m, L[3]);
+    }
+    rp *= rho;
+    { const T m = -__ldg(Mr + 25) * rp;
+      L[0] = m2l_fma(D[31], m, L[0]);
+    }
+    { const T m = -__ldg(Mr + 26) * rp;
+      L[0] = m2l_fma(D[32], m, L[0]);
+    }
+    { const T m = -__ldg(Mr + 27) * rp;
+      L[0] = m2l_fma(D[33], m, L[0]);
+    }
+    { const T m = -__ldg(Mr + 28) * rp;
+      L[0] = m2l_fma(D[34], m, L[0]);
+    }
+    { const T m = -__ldg(Mr + 29) * rp;
+      L[0] = m2l_fma(D[35], m, L[0]);
+    }
+    { const T m = -__ldg(Mr + 30) * rp;
+      L[0] = m2l_fma(D[37], m, L[0]);
+    }
+    { const T m = -__ldg(Mr + 31) * rp;
+      L[0] = m2l_fma(D[38], m, L[0]);
+    }
+    { const T m = -__ldg(Mr + 32) * rp;
+      L[0] = m2l_fma(D[40], m, L[0]);
+    }
+    { const T m = -__ldg(Mr + 33) * rp;
+      L[0] = m2l_fma(D[41], m, L[0]);
+    }
+    { const T m = -__ldg(Mr + 34) * rp;
+      L[0] = m2l_fma(D[43], m, L[0]);
+    }
+    { const T m = -__ldg(Mr + 35) * rp;
+      L[0] = m2l_fma(D[44], m, L[0]);
     }
 }
 
-__device__ __forceinline__ void m2l_acc_h_5(const float (&D)[46], const float *__restrict__ Mr, float rho, float (&L)[36])
+template <class T> __device__ __forceinline__ void m2l_acc_h_5(const T (&D)[46], const T *__restrict__ Mr, T rho, T (&L)[36])
 {
-    float rp = 1.0f;
-    { const float m = __ldg(Mr + 0) * rp;
-      L[0] = fmaf(D[0], m, L[0]);
-      L[1] = fmaf(D[1], m, L[1]);
-      L[2] = fmaf(D[2], m, L[2]);
-      L[3] = fmaf(D[3], m, L[3]);
-      L[4] = fmaf(D[4], m, L[4]);
-      L[5] = fmaf(D[5], m, L[5]);
-      L[6] = fmaf(D[6], m, L[6]);
-      L[7] = fmaf(D[7], m, L[7]);
-      L[8] = fmaf(D[8], m, L[8]);
-      L[9] = fmaf(D[10], m, L[9]);
-      L[10] = fmaf(D[11], m, L[10]);
-      L[11] = fmaf(D[12], m, L[11]);
-      L[12] = fmaf(D[13], m, L[12]);
-      L[13] = fmaf(D[14], m, L[13]);
-      L[14] = fmaf(D[16], m, L[14]);
-      L[15] = fmaf(D[17], m, L[15]);
-      L[16] = fmaf(D[19], m, L[16]);
-      L[17] = fmaf(D[20], m, L[17]);
-      L[18] = fmaf(D[21], m, L[18]);
-      L[19] = fmaf(D[22], m, L[19]);
-      L[20] = fmaf(D[23], m, L[20]);
-      L[21] = fmaf(D[25], m, L[21]);
-      L[22] = fmaf(D[26], m, L[22]);
-      L[23] = fmaf(D[28], m, L[23]);
-      L[24] = fmaf(D[29], m, L[24]);
-      L[25] = fmaf(D[31], m, L[25]);
-      L[26] = fmaf(D[32], m, L[26]);
-      L[27] = fmaf(D[33], m, L[27]);
-      L[28] = fmaf(D[34], m, L[28]);
-      L[29] = fmaf(D[35], m, L[29]);
-      L[30] = fmaf(D[37], m, L[30]);
-      L[31] = fmaf(D[38], m, L[31]);
-      L[32] = fmaf(D[40], m, L[32]);
-      L[33] = fmaf(D[41], m, L[33]);
-      L[34] = fmaf(D[43], m, L[34]);
-      L[35] = fmaf(D[44], m, L[35]);
+    T rp = T(1);
+    { const T m = __ldg(Mr + 0) * rp;
+      L[0] = m2l_fma(D[0], m, L[0]);
+      L[1] = m2l_fma(D[1], m, L[1]);
+      L[2] = m2l_fma(D[2], m, L[2]);
+      L[3] = m2l_fma(D[3], m, L[3]);
+      L[4] = m2l_fma(D[4], m, L[4]);
+      L[5] = m2l_fma(D[5], m, L[5]);
+      L[6] = m2l_fma(D[6], m, L[6]);
+      L[7] = m2l_fma(D[7], m, L[7]);
+      L[8] = m2l_fma(D[8], m, L[8]);
+      L[9] = m2l_fma(D[10], m, L[9]);
+      L[10] = m2l_fma(D[11], m, L[10]);
+      L[11] = m2l_fma(D[12], m, L[11]);
+      L[12] = m2l_fma(D[13], m, L[12]);
+      L[13] = m2l_fma(D[14], m, L[13]);
+      L[14] = m2l_fma(D[16], m, L[14]);
+      L[15] = m2l_fma(D[17], m, L[15]);
+      L[16] = m2l_fma(D[19], m, L[16]);
+      L[17] = m2l_fma(D[20], m, L[17]);
+      L[18] = m2l_fma(D[21], m, L[18]);
+      L[19] = m2l_fma(D[22], m, L[19]);
+      L[20] = m2l_fma(D[23], m, L[20]);
+      L[21] = m2l_fma(D[25], m, L[21]);
+      L[22] = m2l_fma(D[26], m, L[22]);
+      L[23] = m2l_fma(D[28], m, L[23]);
+      L[24] = m2l_fma(D[29], m, L[24]);
+      L[25] = m2l_fma(D[31], m, L[25]);
+      L[26] = m2l_fma(D[32], m, L[26]);
+      L[27] = m2l_fma(D[33], m, L[27]);
+      L[28] = m2l_fma(D[34], m, L[28]);
+      L[29] = m2l_fma(D[35], m, L[29]);
+      L[30] = m2l_fma(D[37], m, L[30]);
+      L[31] = m2l_fma(D[38], m, L[31]);
+      L[32] = m2l_fma(D[40], m, L[32]);
+      L[33] = m2l_fma(D[41], m, L[33]);
+      L[34] = m2l_fma(D[43], m, L[34]);
+      L[35] = m2l_fma(D[44], m, L[35]);
     }
     rp *= rho;
-    { const float m = -__ldg(Mr + 1) * rp;
-      L[0] = fmaf(D[1], m, L[0]);
-      L[1] = fmaf(D[4], m, L[1]);
-      L[2] = fmaf(D[5], m, L[2]);
-      L[3] = fmaf(D[6], m, L[3]);
-      L[4] = fmaf(D[10], m, L[4]);
-      L[5] = fmaf(D[11], m, L[5]);
-      L[6] = fmaf(D[12], m, L[6]);
-      L[7] = fmaf(D[13], m, L[7]);
-      L[8] = fmaf(D[14], m, L[8]);
-      L[9] = fmaf(D[19], m, L[9]);
-      L[10] = fmaf(D[20], m, L[10]);
-      L[11] = fmaf(D[21], m, L[11]);
-      L[12] = fmaf(D[22], m, L[12]);
-      L[13] = fmaf(D[23], m, L[13]);
-      L[14] = fmaf(D[25], m, L[14]);
-      L[15] = fmaf(D[26], m, L[15]);
-      L[16] = fmaf(D[31], m, L[16]);
-      L[17] = fmaf(D[32], m, L[17]);
-      L[18] = fmaf(D[33], m, L[18]);
-      L[19] = fmaf(D[34], m, L[19]);
-      L[20] = fmaf(D[35], m, L[20]);
-      L[21] = fmaf(D[37], m, L[21]);
-      L[22] = fmaf(D[38], m, L[22]);
-      L[23] = fmaf(D[40], m, L[23]);
-      L[24] = fmaf(D[41], m, L[24]);
+    { const T m = -__ldg(Mr + 1) * rp;
+      L[0] = m2l_fma(D[1], m, L[0]);
+      L[1] = m2l_fma(D[4], m, L[1]);
+      L[2] = m2l_fma(D[5], m, L[2]);
+      L[3] = m2l_fma(D[6], m, L[3]);
+      L[4] = m2l_fma(D[10], m, L[4]);
+      L[5] = m2l_fma(D[11], m, L[5]);
+      L[6] = m2l_fma(D[12], m, L[6]);
+      L[7] = m2l_fma(D[13], m, L[7]);
+      L[8] = m2l_fma(D[14], m, L[8]);
+      L[9] = m2l_fma(D[19], m, L[9]);
+      L[10] = m2l_fma(D[20], m, L[10]);
+      L[11] = m2l_fma(D[21], m, L[11]);
+      L[12] = m2l_fma(D[22], m, L[12]);
+      L[13] = m2l_fma(D[23], m, L[13]);
+      L[14] = m2l_fma(D[25], m, L[14]);
+      L[15] = m2l_fma(D[26], m, L[15]);
+      L[16] = m2l_fma(D[31], m, L[16]);
+      L[17] = m2l_fma(D[32], m, L[17]);
+      L[18] = m2l_fma(D[33], m, L[18]);
+      L[19] = m2l_fma(D[34], m, L[19]);
+      L[20] = m2l_fma(D[35], m, L[20]);
+      L[21] = m2l_fma(D[37], m, L[21]);
+      L[22] = m2l_fma(D[38], m, L[22]);
+      L[23] = m2l_fma(D[40], m, L[23]);
+      L[24] = m2l_fma(D[41], m, L[24]);
     }
-    { const float m = -__ldg(Mr + 2) * rp;
-      L[0] = fmaf(D[2], m, L[0]);
-      L[1] = fmaf(D[5], m, L[1]);
-      L[2] = fmaf(D[7], m, L[2]);
-      L[3] = fmaf(D[8], m, L[3]);
-      L[4] = fmaf(D[11], m, L[4]);
-      L[5] = fmaf(D[13], m, L[5]);
-      L[6] = fmaf(D[14], m, L[6]);
-      L[7] = fmaf(D[16], m, L[7]);
-      L[8] = fmaf(D[17], m, L[8]);
-      L[9] = fmaf(D[20], m, L[9]);
-      L[10] = fmaf(D[22], m, L[10]);
-      L[11] = fmaf(D[23], m, L[11]);
-      L[12] = fmaf(D[25], m, L[12]);
-      L[13] = fmaf(D[26], m, L[13]);
-      L[14] = fmaf(D[28], m, L[14]);
-      L[15] = fmaf(D[29], m, L[15]);
-      L[16] = fmaf(D[32], m, L[16]);
-      L[17] = fmaf(D[34], m, L[17]);
-      L[18] = fmaf(D[35], m, L[18]);
-      L[19] = fmaf(D[37], m, L[19]);
-      L[20] = fmaf(D[38], m, L[20]);
-      L[21] = fmaf(D[40], m, L[21]);
-      L[22] = fmaf(D[41], m, L[22]);
-      L[23] = fmaf(D[43], m, L[23]);
-      L[24] = fmaf(D[44], m, L[24]);
+    { const T m = -__ldg(Mr + 2) * rp;
+      L[0] = m2l_fma(D[2], m, L[0]);
+      L[1] = m2l_fma(D[5], m, L[1]);
+      L[2] = m2l_fma(D[7], m, L[2]);
+      L[3] = m2l_fma(D[8], m, L[3]);
+      L[4] = m2l_fma(D[11], m, L[4]);
+      L[5] = m2l_fma(D[13], m, L[5]);
+      L[6] = m2l_fma(D[14], m, L[6]);
+      L[7] = m2l_fma(D[16], m, L[7]);
+      L[8] = m2l_fma(D[17], m, L[8]);
+      L[9] = m2l_fma(D[20], m, L[9]);
+      L[10] = m2l_fma(D[22], m, L[10]);
+      L[11] = m2l_fma(D[23], m, L[11]);
+      L[12] = m2l_fma(D[25], m, L[12]);
+      L[13] = m2l_fma(D[26], m, L[13]);
+      L[14] = m2l_fma(D[28], m, L[14]);
+      L[15] = m2l_fma(D[29], m, L[15]);
+      L[16] = m2l_fma(D[32], m, L[16]);
+      L[17] = m2l_fma(D[34], m, L[17]);
+      L[18] = m2l_fma(D[35], m, L[18]);
+      L[19] = m2l_fma(D[37], m, L[19]);
+      L[20] = m2l_fma(D[38], m, L[20]);
+      L[21] = m2l_fma(D[40], m, L[21]);
+      L[22] = m2l_fma(D[41], m, L[22]);
+      L[23] = m2l_fma(D[43], m, L[23]);
+      L[24] = m2l_fma(D[44], m, L[24]);
     }
-    { const float m = -__ldg(Mr + 3) * rp;
-      L[0] = fmaf(D[3], m, L[0]);
-      L[1] = fmaf(D[6], m, L[1]);
-      L[2] = fmaf(D[8], m, L[2]);
-      L[3] = fmaf(D[9], m, L[3]);
-      L[4] = fmaf(D[12], m, L[4]);
-      L[5] = fmaf(D[14], m, L[5]);
-      L[6] = fmaf(D[15], m, L[6]);
-      L[7] = fmaf(D[17], m, L[7]);
-      L[8] = fmaf(D[18], m, L[8]);
-      L[9] = fmaf(D[21], m, L[9]);
-      L[10] = fmaf(D[23], m, L[10]);
-      L[11] = fmaf(D[24], m, L[11]);
-      L[12] = fmaf(D[26], m, L[12]);
-      L[13] = fmaf(D[27], m, L[13]);
-      L[14] = fmaf(D[29], m, L[14]);
-      L[15] = fmaf(D[30], m, L[15]);
-      L[16] = fmaf(D[33], m, L[16]);
-      L[17] = fmaf(D[35], m, L[17]);
-      L[18] = fmaf(D[36], m, L[18]);
-      L[19] = fmaf(D[38], m, L[19]);
-      L[20] = fmaf(D[39], m, L[20]);
-      L[21] = fmaf(D[41], m, L[21]);
-      L[22] = fmaf(D[42], m, L[22]);
-      L[23] = fmaf(D[44], m, L[23]);
-      L[24] = fmaf(D[45], m, L[24]);
-    }
-    rp *= rho;
-    { const float m = __ldg(Mr + 4) * rp;
-      L[0] = fmaf(D[4], m, L[0]);
-      L[1] = fmaf(D[10], m, L[1]);
-      L[2] = fmaf(D[11], m, L[2]);
-      L[3] = fmaf(D[12], m, L[3]);
-      L[4] = fmaf(D[19], m, L[4]);
-      L[5] = fmaf(D[20], m, L[5]);
-      L[6] = fmaf(D[21], m, L[6]);
-      L[7] = fmaf(D[22], m, L[7]);
-      L[8] = fmaf(D[23], m, L[8]);
-      L[9] = fmaf(D[31], m, L[9]);
-      L[10] = fmaf(D[32], m, L[10]);
-      L[11] = fmaf(D[33], m, L[11]);
-      L[12] = fmaf(D[34], m, L[12]);
-      L[13] = fmaf(D[35], m, L[13]);
-      L[14] = fmaf(D[37], m, L[14]);
-      L[15] = fmaf(D[38], m, L[15]);
-    }
-    { const float m = __ldg(Mr + 5) * rp;
-      L[0] = fmaf(D[5], m, L[0]);
-      L[1] = fmaf(D[11], m, L[1]);
-      L[2] = fmaf(D[13], m, L[2]);
-      L[3] = fmaf(D[14], m, L[3]);
-      L[4] = fmaf(D[20], m, L[4]);
-      L[5] = fmaf(D[22], m, L[5]);
-      L[6] = fmaf(D[23], m, L[6]);
-      L[7] = fmaf(D[25], m, L[7]);
-      L[8] = fmaf(D[26], m, L[8]);
-      L[9] = fmaf(D[32], m, L[9]);
-      L[10] = fmaf(D[34], m, L[10]);
-      L[11] = fmaf(D[35], m, L[11]);
-      L[12] = fmaf(D[37], m, L[12]);
-      L[13] = fmaf(D[38], m, L[13]);
-      L[14] = fmaf(D[40], m, L[14]);
-      L[15] = fmaf(D[41], m, L[15]);
-    }
-    { const float m = __ldg(Mr + 6) * rp;
-      L[0] = fmaf(D[6], m, L[0]);
-      L[1] = fmaf(D[12], m, L[1]);
-      L[2] = fmaf(D[14], m, L[2]);
-      L[3] = fmaf(D[15], m, L[3]);
-      L[4] = fmaf(D[21], m, L[4]);
-      L[5] = fmaf(D[23], m, L[5]);
-      L[6] = fmaf(D[24], m, L[6]);
-      L[7] = fmaf(D[26], m, L[7]);
-      L[8] = fmaf(D[27], m, L[8]);
-      L[9] = fmaf(D[33], m, L[9]);
-      L[10] = fmaf(D[35], m, L[10]);
-      L[11] = fmaf(D[36], m, L[11]);
-      L[12] = fmaf(D[38], m, L[12]);
-      L[13] = fmaf(D[39], m, L[13]);
-      L[14] = fmaf(D[41], m, L[14]);
-      L[15] = fmaf(D[42], m, L[15]);
-    }
-    { const float m = __ldg(Mr + 7) * rp;
-      L[0] = fmaf(D[7], m, L[0]);
-      L[1] = fmaf(D[13], m, L[1]);
-      L[2] = fmaf(D[16], m, L[2]);
-      L[3] = fmaf(D[17], m, L[3]);
-      L[4] = fmaf(D[22], m, L[4]);
-      L[5] = fmaf(D[25], m, L[5]);
-      L[6] = fmaf(D[26], m, L[6]);
-      L[7] = fmaf(D[28], m, L[7]);
-      L[8] = fmaf(D[29], m, L[8]);
-      L[9] = fmaf(D[34], m, L[9]);
-      L[10] = fmaf(D[37], m, L[10]);
-      L[11] = fmaf(D[38], m, L[11]);
-      L[12] = fmaf(D[40], m, L[12]);
-      L[13] = fmaf(D[41], m, L[13]);
-      L[14] = fmaf(D[43], m, L[14]);
-      L[15] = fmaf(D[44], m, L[15]);
-    }
-    { const float m = __ldg(Mr + 8) * rp;
-      L[0] = fmaf(D[8], m, L[0]);
-      L[1] = fmaf(D[14], m, L[1]);
-      L[2] = fmaf(D[17], m, L[2]);
-      L[3] = fmaf(D[18], m, L[3]);
-      L[4] = fmaf(D[23], m, L[4]);
-      L[5] = fmaf(D[26], m, L[5]);
-      L[6] = fmaf(D[27], m, L[6]);
-      L[7] = fmaf(D[29], m, L[7]);
-      L[8] = fmaf(D[30], m, L[8]);
-      L[9] = fmaf(D[35], m, L[9]);
-      L[10] = fmaf(D[38], m, L[10]);
-      L[11] = fmaf(D[39], m, L[11]);
-      L[12] = fmaf(D[41], m, L[12]);
-      L[13] = fmaf(D[42], m, L[13]);
-      L[14] = fmaf(D[44], m, L[14]);
-      L[15] = fmaf(D[45], m, L[15]);
+    { const T m = -__ldg(Mr + 3) * rp;
+      L[0] = m2l_fma(D[3], m, L[0]);
+      L[1] = m2l_fma(D[6], m, L[1]);
+      L[2] = m2l_fma(D[8], m, L[2]);
+      L[3] = m2l_fma(D[9], m, L[3]);
+      L[4] = m2l_fma(D[12], m, L[4]);
+      L[5] = m2l_fma(D[14], m, L[5]);
+      L[6] = m2l_fma(D[15], m, L[6]);
+      L[7] = m2l_fma(D[17], m, L[7]);
+      L[8] = m2l_fma(D[18], m, L[8]);
+      L[9] = m2l_fma(D[21], m, L[9]);
+      L[10] = m2l_fma(D[23], m, L[10]);
+      L[11] = m2l_fma(D[24], m, L[11]);
+      L[12] = m2l_fma(D[26], m, L[12]);
+      L[13] = m2l_fma(D[27], m, L[13]);
+      L[14] = m2l_fma(D[29], m, L[14]);
+      L[15] = m2l_fma(D[30], m, L[15]);
+      L[16] = m2l_fma(D[33], m, L[16]);
+      L[17] = m2l_fma(D[35], m, L[17]);
+      L[18] = m2l_fma(D[36], m, L[18]);
+      L[19] = m2l_fma(D[38], m, L[19]);
+      L[20] = m2l_fma(D[39], m, L[20]);
+      L[21] = m2l_fma(D[41], m, L[21]);
+      L[22] = m2l_fma(D[42], m, L[22]);
+      L[23] = m2l_fma(D[44], m, L[23]);
+      L[24] = m2l_fma(D[45], m, L[24]);
     }
     rp *= rho;
-    { const float m = -__ldg(Mr + 9) * rp;
-      L[0] = fmaf(D[10], m, L[0]);
-      L[1] = fmaf(D[19], m, L[1]);
-      L[2] = fmaf(D[20], m, L[2]);
-      L[3] = fmaf(D[21], m, L[3]);
-      L[4] = fmaf(D[31], m, L[4]);
-      L[5] = fmaf(D[32], m, L[5]);
-      L[6] = fmaf(D[33], m, L[6]);
-      L[7] = fmaf(D[34], m, L[7]);
-      L[8] = fmaf(D[35], m, L[8]);
+    { const T m = __ldg(Mr + 4) * rp;
+      L[0] = m2l_fma(D[4], m, L[0]);
+      L[1] = m2l_fma(D[10], m, L[1]);
+      L[2] = m2l_fma(D[11], m, L[2]);
+      L[3] = m2l_fma(D[12], m, L[3]);
+      L[4] = m2l_fma(D[19], m, L[4]);
+      L[5] = m2l_fma(D[20], m, L[5]);
+      L[6] = m2l_fma(D[21], m, L[6]);
+      L[7] = m2l_fma(D[22], m, L[7]);
+      L[8] = m2l_fma(D[23], m, L[8]);
+      L[9] = m2l_fma(D[31], m, L[9]);
+      L[10] = m2l_fma(D[32], m, L[10]);
+      L[11] = m2l_fma(D[33], m, L[11]);
+      L[12] = m2l_fma(D[34], m, L[12]);
+      L[13] = m2l_fma(D[35], m, L[13]);
+      L[14] = m2l_fma(D[37], m, L[14]);
+      L[15] = m2l_fma(D[38], m, L[15]);
     }
-    { const float m = -__ldg(Mr + 10) * rp;
-      L[0] = fmaf(D[11], m, L[0]);
-      L[1] = fmaf(D[20], m, L[1]);
-      L[2] = fmaf(D[22], m, L[2]);
-      L[3] = fmaf(D[23], m, L[3]);
-      L[4] = fmaf(D[32], m, L[4]);
-      L[5] = fmaf(D[34], m, L[5]);
-      L[6] = fmaf(D[35], m, L[6]);
-      L[7] = fmaf(D[37], m, L[7]);
-      L[8] = fmaf(D[38], m, L[8]);
+    { const T m = __ldg(Mr + 5) * rp;
+      L[0] = m2l_fma(D[5], m, L[0]);
+      L[1] = m2l_fma(D[11], m, L[1]);
+      L[2] = m2l_fma(D[13], m, L[2]);
+      L[3] = m2l_fma(D[14], m, L[3]);
+      L[4] = m2l_fma(D[20], m, L[4]);
+      L[5] = m2l_fma(D[22], m, L[5]);
+      L[6] = m2l_fma(D[23], m, L[6]);
+      L[7] = m2l_fma(D[25], m, L[7]);
+      L[8] = m2l_fma(D[26], m, L[8]);
+      L[9] = m2l_fma(D[32], m, L[9]);
+      L[10] = m2l_fma(D[34], m, L[10]);
+      L[11] = m2l_fma(D[35], m, L[11]);
+      L[12] = m2l_fma(D[37], m, L[12]);
+      L[13] = m2l_fma(D[38], m, L[13]);
+      L[14] = m2l_fma(D[40], m, L[14]);
+      L[15] = m2l_fma(D[41], m, L[15]);
     }
-    { const float m = -__ldg(Mr + 11) * rp;
-      L[0] = fmaf(D[12], m, L[0]);
-      L[1] = fmaf(D[21], m, L[1]);
-      L[2] = fmaf(D[23], m, L[2]);
-      L[3] = fmaf(D[24], m, L[3]);
-      L[4] = fmaf(D[33], m, L[4]);
-      L[5] = fmaf(D[35], m, L[5]);
-      L[6] = fmaf(D[36], m, L[6]);
-      L[7] = fmaf(D[38], m, L[7]);
-      L[8] = fmaf(D[39], m, L[8]);
+    { const T m = __ldg(Mr + 6) * rp;
+      L[0] = m2l_fma(D[6], m, L[0]);
+      L[1] = m2l_fma(D[12], m, L[1]);
+      L[2] = m2l_fma(D[14], m, L[2]);
+      L[3] = m2l_fma(D[15], m, L[3]);
+      L[4] = m2l_fma(D[21], m, L[4]);
+      L[5] = m2l_fma(D[23], m, L[5]);
+      L[6] = m2l_fma(D[24], m, L[6]);
+      L[7] = m2l_fma(D[26], m, L[7]);
+      L[8] = m2l_fma(D[27], m, L[8]);
+      L[9] = m2l_fma(D[33], m, L[9]);
+      L[10] = m2l_fma(D[35], m, L[10]);
+      L[11] = m2l_fma(D[36], m, L[11]);
+      L[12] = m2l_fma(D[38], m, L[12]);
+      L[13] = m2l_fma(D[39], m, L[13]);
+      L[14] = m2l_fma(D[41], m, L[14]);
+      L[15] = m2l_fma(D[42], m, L[15]);
     }
-    { const float m = -__ldg(Mr + 12) * rp;
-      L[0] = fmaf(D[13], m, L[0]);
-      L[1] = fmaf(D[22], m, L[1]);
-      L[2] = fmaf(D[25], m, L[2]);
-      L[3] = fmaf(D[26], m, L[3]);
-      L[4] = fmaf(D[34], m, L[4]);
-      L[5] = fmaf(D[37], m, L[5]);
-      L[6] = fmaf(D[38], m, L[6]);
-      L[7] = fmaf(D[40], m, L[7]);
-      L[8] = fmaf(D[41], m, L[8]);
+    { const T m = __ldg(Mr + 7) * rp;
+      L[0] = m2l_fma(D[7], m, L[0]);
+      L[1] = m2l_fma(D[13], m, L[1]);
+      L[2] = m2l_fma(D[16], m, L[2]);
+      L[3] = m2l_fma(D[17], m, L[3]);
+      L[4] = m2l_fma(D[22], m, L[4]);
+      L[5] = m2l_fma(D[25], m, L[5]);
+      L[6] = m2l_fma(D[26], m, L[6]);
+      L[7] = m2l_fma(D[28], m, L[7]);
+      L[8] = m2l_fma(D[29], m, L[8]);
+      L[9] = m2l_fma(D[34], m, L[9]);
+      L[10] = m2l_fma(D[37], m, L[10]);
+      L[11] = m2l_fma(D[38], m, L[11]);
+      L[12] = m2l_fma(D[40], m, L[12]);
+      L[13] = m2l_fma(D[41], m, L[13]);
+      L[14] = m2l_fma(D[43], m, L[14]);
+      L[15] = m2l_fma(D[44], m, L[15]);
     }
-    { const float m = -__ldg(Mr + 13) * rp;
-      L[0] = fmaf(D[14], m, L[0]);
-      L[1] = fmaf(D[23], m, L[1]);
-      L[2] = fmaf(D[26], m, L[2]);
-      L[3] = fmaf(D[27], m, L[3]);
-      L[4] = fmaf(D[35], m, L[4]);
-      L[5] = fmaf(D[38], m, L[5]);
-      L[6] = fmaf(D[39], m, L[6]);
-      L[7] = fmaf(D[41], m, L[7]);
-      L[8] = fmaf(D[42], m, L[8]);
-    }
-    { const float m = -__ldg(Mr + 14) * rp;
-      L[0] = fmaf(D[16], m, L[0]);
-      L[1] = fmaf(D[25], m, L[1]);
-      L[2] = fmaf(D[28], m, L[2]);
-      L[3] = fmaf(D[29], m, L[3]);
-      L[4] = fmaf(D[37], m, L[4]);
-      L[5] = fmaf(D[40], m, L[5]);
-      L[6] = fmaf(D[41], m, L[6]);
-      L[7] = fmaf(D[43], m, L[7]);
-      L[8] = fmaf(D[44], m, L[8]);
-    }
-    { const float m = -__ldg(Mr + 15) * rp;
-      L[0] = fmaf(D[17], m, L[0]);
-      L[1] = fmaf(D[26], m, L[1]);
-      L[2] = fmaf(D[29], m, L[2]);
-      L[3] = fmaf(D[30], m, L[3]);
-      L[4] = fmaf(D[38], m, L[4]);
-      L[5] = fmaf(D[41], m, L[5]);
-      L[6] = fmaf(D[42], m, L[6]);
-      L[7] = fmaf(D[44], m, L[7]);
-      L[8] = fmaf(D[45], m, L[8]);
-    }
-    rp *= rho;
-    { const float m = __ldg(Mr + 16) * rp;
-      L[0] = fmaf(D[19], m, L[0]);
-      L[1] = fmaf(D[31], m, L[1]);
-      L[2] = fmaf(D[32], m, L[2]);
-      L[3] = fmaf(D[33], m, L[3]);
-    }
-    { const float m = __ldg(Mr + 17) * rp;
-      L[0] = fmaf(D[20], m, L[0]);
-      L[1] = fmaf(D[32], m, L[1]);
-      L[2] = fmaf(D[34], m, L[2]);
-      L[3] = fmaf(D[35], m, L[3]);
-    }
-    { const float m = __ldg(Mr + 18) * rp;
-      L[0] = fmaf(D[21], m, L[0]);
-      L[1] = fmaf(D[33], m, L[1]);
-      L[2] = fmaf(D[35], m, L[2]);
-      L[3] = fmaf(D[36], m, L[3]);
-    }
-    { const float m = __ldg(Mr + 19) * rp;
-      L[0] = fmaf(D[22], m, L[0]);
-      L[1] = fmaf(D[34], m, L[1]);
-      L[2] = fmaf(D[37], m, L[2]);
-      L[3] = fmaf(D[38], m, L[3]);
-    }
-    { const float m = __ldg(Mr + 20) * rp;
-      L[0] = fmaf(D[23], m, L[0]);
-      L[1] = fmaf(D[35], m, L[1]);
-      L[2] = fmaf(D[38], m, L[2]);
-      L[3] = fmaf(D[39], m, L[3]);
-    }
-    { const float m = __ldg(Mr + 21) * rp;
-      L[0] = fmaf(D[25], m, L[0]);
-      L[1] = fmaf(D[37], m, L[1]);
-      L[2] = fmaf(D[40], m, L[2]);
-      L[3] = fmaf(D[41], m, L[3]);
-    }
-    { const float m = __ldg(Mr + 22) * rp;
-      L[0] = fmaf(D[26], m, L[0]);
-      L[1] = fmaf(D[38], m, L[1]);
-      L[2] = fmaf(D[41], m, L[2]);
-      L[3] = fmaf(D[42], m, L[3]);
-    }
-    { const float m = __ldg(Mr + 23) * rp;
-      L[0] = fmaf(D[28], m, L[0]);
-      L[1] = fmaf(D[40], m, L[1]);
-      L[2] = fmaf(D[43], m, L[2]);
-      L[3] = fmaf(D[44], m, L[3]);
-    }
-    { const float m = __ldg(Mr + 24) * rp;
-      L[0] = fmaf(D[29], m, L[0]);
-      L[1] = fmaf(D[41], m, L[1]);
-      L[2] = fmaf(D[44], m, L[2]);
-      L[3] = fmaf(D[45], m, L[3]);
+    { const T m = __ldg(Mr + 8) * rp;
+      L[0] = m2l_fma(D[8], m, L[0]);
+      L[1] = m2l_fma(D[14], m, L[1]);
+      L[2] = m2l_fma(D[17], m, L[2]);
+      L[3] = m2l_fma(D[18], m, L[3]);
+      L[4] = m2l_fma(D[23], m, L[4]);
+      L[5] = m2l_fma(D[26], m, L[5]);
+      L[6] = m2l_fma(D[27], m, L[6]);
+      L[7] = m2l_fma(D[29], m, L[7]);
+      L[8] = m2l_fma(D[30], m, L[8]);
+      L[9] = m2l_fma(D[35], m, L[9]);
+      L[10] = m2l_fma(D[38], m, L[10]);
+      L[11] = m2l_fma(D[39], m, L[11]);
+      L[12] = m2l_fma(D[41], m, L[12]);
+      L[13] = m2l_fma(D[42], m, L[13]);
+      L[14] = m2l_fma(D[44], m, L[14]);
+      L[15] = m2l_fma(D[45], m, L[15]);
     }
     rp *= rho;
-    { const float m = -__ldg(Mr + 25) * rp;
-      L[0] = fmaf(D[31], m, L[0]);
+    { const T m = -__ldg(Mr + 9) * rp;
+      L[0] = m2l_fma(D[10], m, L[0]);
+      L[1] = m2l_fma(D[19], m, L[1]);
+      L[2] = m2l_fma(D[20], m, L[2]);
+      L[3] = m2l_fma(D[21], m, L[3]);
+      L[4] = m2l_fma(D[31], m, L[4]);
+      L[5] = m2l_fma(D[32], m, L[5]);
+      L[6] = m2l_fma(D[33], m, L[6]);
+      L[7] = m2l_fma(D[34], m, L[7]);
+      L[8] = m2l_fma(D[35], m, L[8]);
     }
-    { const float m = -__ldg(Mr + 26) * rp;
-      L[0] = fmaf(D[32], m, L[0]);
+    { const T m = -__ldg(Mr + 10) * rp;
+      L[0] = m2l_fma(D[11], m, L[0]);
+      L[1] = m2l_fma(D[20], m, L[1]);
+      L[2] = m2l_fma(D[22], m, L[2]);
+      L[3] = m2l_fma(D[23], m, L[3]);
+      L[4] = m2l_fma(D[32], m, L[4]);
+      L[5] = m2l_fma(D[34], m, L[5]);
+      L[6] = m2l_fma(D[35], m, L[6]);
+      L[7] = m2l_fma(D[37], m, L[7]);
+      L[8] = m2l_fma(D[38], m, L[8]);
     }
-    { const float m = -__ldg(Mr + 27) * rp;
-      L[0] = fmaf(D[33], m, L[0]);
+    { const T m = -__ldg(Mr + 11) * rp;
+      L[0] = m2l_fma(D[12], m, L[0]);
+      L[1] = m2l_fma(D[21], m, L[1]);
+      L[2] = m2l_fma(D[23], m, L[2]);
+      L[3] = m2l_fma(D[24], m, L[3]);
+      L[4] = m2l_fma(D[33], m, L[4]);
+      L[5] = m2l_fma(D[35], m, L[5]);
+      L[6] = m2l_fma(D[36], m, L[6]);
+      L[7] = m2l_fma(D[38], m, L[7]);
+      L[8] = m2l_fma(D[39], m, L[8]);
     }
-    { const float m = -__ldg(Mr + 28) * rp;
-      L[0] = fmaf(D[34], m, L[0]);
+    { const T m = -__ldg(Mr + 12) * rp;
+      L[0] = m2l_fma(D[13], m, L[0]);
+      L[1] = m2l_fma(D[22], m, L[1]);
+      L[2] = m2l_fma(D[25], m, L[2]);
+      L[3] = m2l_fma(D[26], m, L[3]);
+      L[4] = m2l_fma(D[34], m, L[4]);
+      L[5] = m2l_fma(D[37], m, L[5]);
+      L[6] = m2l_fma(D[38], m, L[6]);
+      L[7] = m2l_fma(D[40], m, L[7]);
+      L[8] = m2l_fma(D[41], m, L[8]);
     }
-    { const float m = -__ldg(Mr + 29) * rp;
-      L[0] = fmaf(D[35], m, L[0]);
+    { const T m = -__ldg(Mr + 13) * rp;
+      L[0] = m2l_fma(D[14], m, L[0]);
+      L[1] = m2l_fma(D[23], m, L[1]);
+      L[2] = m2l_fma(D[26], m, L[2]);
+      L[3] = m2l_fma(D[27], m, L[3]);
+      L[4] = m2l_fma(D[35], m, L[4]);
+      L[5] = m2l_fma(D[38], m, L[5]);
+      L[6] = m2l_fma(D[39], m, L[6]);
+      L[7] = m2l_fma(D[41], m, L[7]);
+      L[8] = m2l_fma(D[42], m, L[8]);
     }
-    { const float m = -__ldg(Mr + 30) * rp;
-      L[0] = fmaf(D[37], m, L[0]);
+    { const T m = -__ldg(Mr + 14) * rp;
+      L[0] = m2l_fma(D[16], m, L[0]);
+      L[1] = m2l_fma(D[25], m, L[1]);
+      L[2] = m2l_fma(D[28], m, L[2]);
+      L[3] = m2l_fma(D[29], m, L[3]);
+      L[4] = m2l_fma(D[37], m, L[4]);
+      L[5] = m2l_fma(D[40], m, L[5]);
+      L[6] = m2l_fma(D[41], m, L[6]);
+      L[7] = m2l_fma(D[43], m, L[7]);
+      L[8] = m2l_fma(D[44], m, L[8]);
     }
-    { const float m = -__ldg(Mr + 31) * rp;
-      L[0] = fmaf(D[38], m, L[0]);
+    { const T m = -__ldg(Mr + 15) * rp;
+      L[0] = m2l_fma(D[17], m, L[0]);
+      L[1] = m2l_fma(D[26], m, L[1]);
+      L[2] = m2l_fma(D[29], m, L[2]);
+      L[3] = m2l_fma(D[30], m, L[3]);
+      L[4] = m2l_fma(D[38], m, L[4]);
+      L[5] = m2l_fma(D[41], m, L[5]);
+      L[6] = m2l_fma(D[42], m, L[6]);
+      L[7] = m2l_fma(D[44], m, L[7]);
+      L[8] = m2l_fma(D[45], m, L[8]);
     }
-    { const float m = -__ldg(Mr + 32) * rp;
-      L[0] = fmaf(D[40], m, L[0]);
+    rp *= rho;
+    { const T m = __ldg(Mr + 16) * rp;
+      L[0] = m2l_fma(D[19], m, L[0]);
+      L[1] = m2l_fma(D[31], m, L[1]);
+      L[2] = m2l_fma(D[32], m, L[2]);
+      L[3] = m2l_fma(D[33], m, L[3]);
     }
-    { const float m = -__ldg(Mr + 33) * rp;
-      L[0] = fmaf(D[41], m, L[0]);
+    { const T m = __ldg(Mr + 17) * rp;
+      L[0] = m2l_fma(D[20], m, L[0]);
+      L[1] = m2l_fma(D[32], m, L[1]);
+      L[2] = m2l_fma(D[34], m, L[2]);
+      L[3] = m2l_fma(D[35], m, L[3]);
     }
-    { const float m = -__ldg(Mr + 34) * rp;
-      L[0] = fmaf(D[43], m, L[0]);
+    { const T m = __ldg(Mr + 18) * rp;
+      L[0] = m2l_fma(D[21], m, L[0]);
+      L[1] = m2l_fma(D[33], m, L[1]);
+      L[2] = m2l_fma(D[35], m, L[2]);
+      L[3] = m2l_fma(D[36], m, L[3]);
     }
-    { const float m = -__ldg(Mr + 35) * rp;
-      L[0] = fmaf(D[44], m, L[0]);
+    { const T m = __ldg(Mr + 19) * rp;
+      L[0] = m2l_fma(D[22], m, L[0]);
+      L[1] = m2l_fma(D[34], m, L[1]);
+      L[2] = m2l_fma(D[37], m, L[2]);
+      L[3] = m2l_fma(D[38], m, L[3]);
+    }
+    { const T m = __ldg(Mr + 20) * rp;
+      L[0] = m2l_fma(D[23], m, L[0]);
+      L[1] = m2l_fma(D[35], m, L[1]);
+      L[2] = m2l_fma(D[38], m, L[2]);
+      L[3] = m2l_fma(D[39], m, L[3]);
+    }
+    { const T m = __ldg(Mr + 21) * rp;
+      L[0] = m2l_fma(D[25], m, L[0]);
+      L[1] = m2l_fma(D[37], m, L[1]);
+      L[2] = m2l_fma(D[40], m, L[2]);
+      L[3] = m2l_fma(D[41], m, L[3]);
+    }
+    { const T m = __ldg(Mr + 22) * rp;
+      L[0] = m2l_fma(D[26], m, L[0]);
+      L[1] = m2l_fma(D[38], m, L[1]);
+      L[2] = m2l_fma(D[41], m, L[2]);
+      L[3] = m2l_fma(D[42], m, L[3]);
+    }
+    { const T m = __ldg(Mr + 23) * rp;
+      L[0] = m2l_fma(D[28], m, L[0]);
+      L[1] = m2l_fma(D[40], m, L[1]);
+      L[2] = m2l_fma(D[43], m, L[2]);
+      L[3] = m2l_fma(D[44], m, L[3]);
+    }
+    { const T m = __ldg(Mr + 24) * rp;
+      L[0] = m2l_fma(D[29], m, L[0]);
+      L[1] = m2l_fma(D[41], m, L[1]);
+      L[2] = m2l_fma(D[44], m, L[2]);
+      L[3] = m2l_fma(D[45], m, L[3]);
+    }
+    rp *= rho;
+    { const T m = -__ldg(Mr + 25) * rp;
+      L[0] = m2l_fma(D[31], m, L[0]);
+    }
+    { const T m = -__ldg(Mr + 26) * rp;
+      L[0] = m2l_fma(D[32], m, L[0]);
+    }
+    { const T m = -__ldg(Mr + 27) * rp;
+      L[0] = m2l_fma(D[33], m, L[0]);
+    }
+    { const T m = -__ldg(Mr + 28) * rp;
+      L[0] = m2l_fma(D[34], m, L[0]);
+    }
+    { const T m = -__ldg(Mr + 29) * rp;
+      L[0] = m2l_fma(D[35], m, L[0]);
+    }
+    { const T m = -__ldg(Mr + 30) * rp;
+      L[0] = m2l_fma(D[37], m, L[0]);
+    }
+    { const T m = -__ldg(Mr + 31) * rp;
+      L[0] = m2l_fma(D[38], m, L[0]);
+    }
+    { const T m = -__ldg(Mr + 32) * rp;
+      L[0] = m2l_fma(D[40], m, L[0]);
+    }
+    { const T m = -__ldg(Mr + 33) * rp;
+      L[0] = m2l_fma(D[41], m, L[0]);
+    }
+    { const T m = -__ldg(Mr + 34) * rp;
+      L[0] = m2l_fma(D[43], m, L[0]);
+    }
+    { const T m = -__ldg(Mr + 35) * rp;
+      L[0] = m2l_fma(D[44], m, L[0]);
     }
 }
 
-__device__ __forceinline__ void m2l_side_b_h_5(const float (&D)[46], const float *__restrict__ Mr, float (&L)[36])
+template <class T> __device__ __forceinline__ void m2l_side_b_h_5(const T (&D)[46], const T *__restrict__ Mr, T (&L)[36])
 {
-    { const float m = __ldg(Mr + 0);
+    { const T m = __ldg(Mr + 0);
       L[0] = D[0] * m;
       L[1] = -D[1] * m;
       L[2] = -D[2] * m;
@@ -12199,348 +12199,348 @@ __device__ __forceinline__ void m2l_side_b_h_5(const float (&D)[46], const float
       L[34] = -D[43] * m;
       L[35] = -D[44] * m;
     }
-    { const float m = __ldg(Mr + 1);
-      L[0] = fmaf(D[1], m, L[0]);
-      L[1] = fmaf(-D[4], m, L[1]);
-      L[2] = fmaf(-D[5], m, L[2]);
-      L[3] = fmaf(-D[6], m, L[3]);
-      L[4] = fmaf(D[10], m, L[4]);
-      L[5] = fmaf(D[11], m, L[5]);
-      L[6] = fmaf(D[12], m, L[6]);
-      L[7] = fmaf(D[13], m, L[7]);
-      L[8] = fmaf(D[14], m, L[8]);
-      L[9] = fmaf(-D[19], m, L[9]);
-      L[10] = fmaf(-D[20], m, L[10]);
-      L[11] = fmaf(-D[21], m, L[11]);
-      L[12] = fmaf(-D[22], m, L[12]);
-      L[13] = fmaf(-D[23], m, L[13]);
-      L[14] = fmaf(-D[25], m, L[14]);
-      L[15] = fmaf(-D[26], m, L[15]);
-      L[16] = fmaf(D[31], m, L[16]);
-      L[17] = fmaf(D[32], m, L[17]);
-      L[18] = fmaf(D[33], m, L[18]);
-      L[19] = fmaf(D[34], m, L[19]);
-      L[20] = fmaf(D[35], m, L[20]);
-      L[21] = fmaf(D[37], m, L[21]);
-      L[22] = fmaf(D[38], m, L[22]);
-      L[23] = fmaf(D[40], m, L[23]);
-      L[24] = fmaf(D[41], m, L[24]);
+    { const T m = __ldg(Mr + 1);
+      L[0] = m2l_fma(D[1], m, L[0]);
+      L[1] = m2l_fma(-D[4], m, L[1]);
+      L[2] = m2l_fma(-D[5], m, L[2]);
+      L[3] = m2l_fma(-D[6], m, L[3]);
+      L[4] = m2l_fma(D[10], m, L[4]);
+      L[5] = m2l_fma(D[11], m, L[5]);
+      L[6] = m2l_fma(D[12], m, L[6]);
+      L[7] = m2l_fma(D[13], m, L[7]);
+      L[8] = m2l_fma(D[14], m, L[8]);
+      L[9] = m2l_fma(-D[19], m, L[9]);
+      L[10] = m2l_fma(-D[20], m, L[10]);
+      L[11] = m2l_fma(-D[21], m, L[11]);
+      L[12] = m2l_fma(-D[22], m, L[12]);
+      L[13] = m2l_fma(-D[23], m, L[13]);
+      L[14] = m2l_fma(-D[25], m, L[14]);
+      L[15] = m2l_fma(-D[26], m, L[15]);
+      L[16] = m2l_fma(D[31], m, L[16]);
+      L[17] = m2l_fma(D[32], m, L[17]);
+      L[18] = m2l_fma(D[33], m, L[18]);
+      L[19] = m2l_fma(D[34], m, L[19]);
+      L[20] = m2l_fma(D[35], m, L[20]);
+      L[21] = m2l_fma(D[37], m, L[21]);
+      L[22] = m2l_fma(D[38], m, L[22]);
+      L[23] = m2l_fma(D[40], m, L[23]);
+      L[24] = m2l_fma(D[41], m, L[24]);
     }
-    { const float m = __ldg(Mr + 2);
-      L[0] = fmaf(D[2], m, L[0]);
-      L[1] = fmaf(-D[5], m, L[1]);
-      L[2] = fmaf(-D[7], m, L[2]);
-      L[3] = fmaf(-D[8], m, L[3]);
-      L[4] = fmaf(D[11], m, L[4]);
-      L[5] = fmaf(D[13], m, L[5]);
-      L[6] = fmaf(D[14], m, L[6]);
-      L[7] = fmaf(D[16], m, L[7]);
-      L[8] = fmaf(D[17], m, L[8]);
-      L[9] = fmaf(-D[20], m, L[9]);
-      L[10] = fmaf(-D[22], m, L[10]);
-      L[11] = fmaf(-D[23], m, L[11]);
-      L[12] = fmaf(-D[25], m, L[12]);
-      L[13] = fmaf(-D[26], m, L[13]);
-      L[14] = fmaf(-D[28], m, L[14]);
-      L[15] = fmaf(-D[29], m, L[15]);
-      L[16] = fmaf(D[32], m, L[16]);
-      L[17] = fmaf(D[34], m, L[17]);
-      L[18] = fmaf(D[35], m, L[18]);
-      L[19] = fmaf(D[37], m, L[19]);
-      L[20] = fmaf(D[38], m, L[20]);
-      L[21] = fmaf(D[40], m, L[21]);
-      L[22] = fmaf(D[41], m, L[22]);
-      L[23] = fmaf(D[43], m, L[23]);
-      L[24] = fmaf(D[44], m, L[24]);
+    { const T m = __ldg(Mr + 2);
+      L[0] = m2l_fma(D[2], m, L[0]);
+      L[1] = m2l_fma(-D[5], m, L[1]);
+      L[2] = m2l_fma(-D[7], m, L[2]);
+      L[3] = m2l_fma(-D[8], m, L[3]);
+      L[4] = m2l_fma(D[11], m, L[4]);
+      L[5] = m2l_fma(D[13], m, L[5]);
+      L[6] = m2l_fma(D[14], m, L[6]);
+      L[7] = m2l_fma(D[16], m, L[7]);
+      L[8] = m2l_fma(D[17], m, L[8]);
+      L[9] = m2l_fma(-D[20], m, L[9]);
+      L[10] = m2l_fma(-D[22], m, L[10]);
+      L[11] = m2l_fma(-D[23], m, L[11]);
+      L[12] = m2l_fma(-D[25], m, L[12]);
+      L[13] = m2l_fma(-D[26], m, L[13]);
+      L[14] = m2l_fma(-D[28], m, L[14]);
+      L[15] = m2l_fma(-D[29], m, L[15]);
+      L[16] = m2l_fma(D[32], m, L[16]);
+      L[17] = m2l_fma(D[34], m, L[17]);
+      L[18] = m2l_fma(D[35], m, L[18]);
+      L[19] = m2l_fma(D[37], m, L[19]);
+      L[20] = m2l_fma(D[38], m, L[20]);
+      L[21] = m2l_fma(D[40], m, L[21]);
+      L[22] = m2l_fma(D[41], m, L[22]);
+      L[23] = m2l_fma(D[43], m, L[23]);
+      L[24] = m2l_fma(D[44], m, L[24]);
     }
-    { const float m = __ldg(Mr + 3);
-      L[0] = fmaf(D[3], m, L[0]);
-      L[1] = fmaf(-D[6], m, L[1]);
-      L[2] = fmaf(-D[8], m, L[2]);
-      L[3] = fmaf(-D[9], m, L[3]);
-      L[4] = fmaf(D[12], m, L[4]);
-      L[5] = fmaf(D[14], m, L[5]);
-      L[6] = fmaf(D[15], m, L[6]);
-      L[7] = fmaf(D[17], m, L[7]);
-      L[8] = fmaf(D[18], m, L[8]);
-      L[9] = fmaf(-D[21], m, L[9]);
-      L[10] = fmaf(-D[23], m, L[10]);
-      L[11] = fmaf(-D[24], m, L[11]);
-      L[12] = fmaf(-D[26], m, L[12]);
-      L[13] = fmaf(-D[27], m, L[13]);
-      L[14] = fmaf(-D[29], m, L[14]);
-      L[15] = fmaf(-D[30], m, L[15]);
-      L[16] = fmaf(D[33], m, L[16]);
-      L[17] = fmaf(D[35], m, L[17]);
-      L[18] = fmaf(D[36], m, L[18]);
-      L[19] = fmaf(D[38], m, L[19]);
-      L[20] = fmaf(D[39], m, L[20]);
-      L[21] = fmaf(D[41], m, L[21]);
-      L[22] = fmaf(D[42], m, L[22]);
-      L[23] = fmaf(D[44], m, L[23]);
-      L[24] = fmaf(D[45], m, L[24]);
+    { const T m = __ldg(Mr + 3);
+      L[0] = m2l_fma(D[3], m, L[0]);
+      L[1] = m2l_fma(-D[6], m, L[1]);
+      L[2] = m2l_fma(-D[8], m, L[2]);
+      L[3] = m2l_fma(-D[9], m, L[3]);
+      L[4] = m2l_fma(D[12], m, L[4]);
+      L[5] = m2l_fma(D[14], m, L[5]);
+      L[6] = m2l_fma(D[15], m, L[6]);
+      L[7] = m2l_fma(D[17], m, L[7]);
+      L[8] = m2l_fma(D[18], m, L[8]);
+      L[9] = m2l_fma(-D[21], m, L[9]);
+      L[10] = m2l_fma(-D[23], m, L[10]);
+      L[11] = m2l_fma(-D[24], m, L[11]);
+      L[12] = m2l_fma(-D[26], m, L[12]);
+      L[13] = m2l_fma(-D[27], m, L[13]);
+      L[14] = m2l_fma(-D[29], m, L[14]);
+      L[15] = m2l_fma(-D[30], m, L[15]);
+      L[16] = m2l_fma(D[33], m, L[16]);
+      L[17] = m2l_fma(D[35], m, L[17]);
+      L[18] = m2l_fma(D[36], m, L[18]);
+      L[19] = m2l_fma(D[38], m, L[19]);
+      L[20] = m2l_fma(D[39], m, L[20]);
+      L[21] = m2l_fma(D[41], m, L[21]);
+      L[22] = m2l_fma(D[42], m, L[22]);
+      L[23] = m2l_fma(D[44], m, L[23]);
+      L[24] = m2l_fma(D[45], m, L[24]);
     }
-    { const float m = __ldg(Mr + 4);
-      L[0] = fmaf(D[4], m, L[0]);
-      L[1] = fmaf(-D[10], m, L[1]);
-      L[2] = fmaf(-D[11], m, L[2]);
-      L[3] = fmaf(-D[12], m, L[3]);
-      L[4] = fmaf(D[19], m, L[4]);
-      L[5] = fmaf(D[20], m, L[5]);
-      L[6] = fmaf(D[21], m, L[6]);
-      L[7] = fmaf(D[22], m, L[7]);
-      L[8] = fmaf(D[23], m, L[8]);
-      L[9] = fmaf(-D[31], m, L[9]);
-      L[10] = fmaf(-D[32], m, L[10]);
-      L[11] = fmaf(-D[33], m, L[11]);
-      L[12] = fmaf(-D[34], m, L[12]);
-      L[13] = fmaf(-D[35], m, L[13]);
-      L[14] = fmaf(-D[37], m, L[14]);
-      L[15] = fmaf(-D[38], m, L[15]);
+    { const T m = __ldg(Mr + 4);
+      L[0] = m2l_fma(D[4], m, L[0]);
+      L[1] = m2l_fma(-D[10], m, L[1]);
+      L[2] = m2l_fma(-D[11], m, L[2]);
+      L[3] = m2l_fma(-D[12], m, L[3]);
+      L[4] = m2l_fma(D[19], m, L[4]);
+      L[5] = m2l_fma(D[20], m, L[5]);
+      L[6] = m2l_fma(D[21], m, L[6]);
+      L[7] = m2l_fma(D[22], m, L[7]);
+      L[8] = m2l_fma(D[23], m, L[8]);
+      L[9] = m2l_fma(-D[31], m, L[9]);
+      L[10] = m2l_fma(-D[32], m, L[10]);
+      L[11] = m2l_fma(-D[33], m, L[11]);
+      L[12] = m2l_fma(-D[34], m, L[12]);
+      L[13] = m2l_fma(-D[35], m, L[13]);
+      L[14] = m2l_fma(-D[37], m, L[14]);
+      L[15] = m2l_fma(-D[38], m, L[15]);
     }
-    { const float m = __ldg(Mr + 5);
-      L[0] = fmaf(D[5], m, L[0]);
-      L[1] = fmaf(-D[11], m, L[1]);
-      L[2] = fmaf(-D[13], m, L[2]);
-      L[3] = fmaf(-D[14], m, L[3]);
-      L[4] = fmaf(D[20], m, L[4]);
-      L[5] = fmaf(D[22], m, L[5]);
-      L[6] = fmaf(D[23], m, L[6]);
-      L[7] = fmaf(D[25], m, L[7]);
-      L[8] = fmaf(D[26], m, L[8]);
-      L[9] = fmaf(-D[32], m, L[9]);
-      L[10] = fmaf(-D[34], m, L[10]);
-      L[11] = fmaf(-D[35], m, L[11]);
-      L[12] = fmaf(-D[37], m, L[12]);
-      L[13] = fmaf(-D[38], m, L[13]);
-      L[14] = fmaf(-D[40], m, L[14]);
-      L[15] = fmaf(-D[41], m, L[15]);
+    { const T m = __ldg(Mr + 5);
+      L[0] = m2l_fma(D[5], m, L[0]);
+      L[1] = m2l_fma(-D[11], m, L[1]);
+      L[2] = m2l_fma(-D[13], m, L[2]);
+      L[3] = m2l_fma(-D[14], m, L[3]);
+      L[4] = m2l_fma(D[20], m, L[4]);
+      L[5] = m2l_fma(D[22], m, L[5]);
+      L[6] = m2l_fma(D[23], m, L[6]);
+      L[7] = m2l_fma(D[25], m, L[7]);
+      L[8] = m2l_fma(D[26], m, L[8]);
+      L[9] = m2l_fma(-D[32], m, L[9]);
+      L[10] = m2l_fma(-D[34], m, L[10]);
+      L[11] = m2l_fma(-D[35], m, L[11]);
+      L[12] = m2l_fma(-D[37], m, L[12]);
+      L[13] = m2l_fma(-D[38], m, L[13]);
+      L[14] = m2l_fma(-D[40], m, L[14]);
+      L[15] = m2l_fma(-D[41], m, L[15]);
     }
-    { const float m = __ldg(Mr + 6);
-      L[0] = fmaf(D[6], m, L[0]);
-      L[1] = fmaf(-D[12], m, L[1]);
-      L[2] = fmaf(-D[14], m, L[2]);
-      L[3] = fmaf(-D[15], m, L[3]);
-      L[4] = fmaf(D[21], m, L[4]);
-      L[5] = fmaf(D[23], m, L[5]);
-      L[6] = fmaf(D[24], m, L[6]);
-      L[7] = fmaf(D[26], m, L[7]);
-      L[8] = fmaf(D[27], m, L[8]);
-      L[9] = fmaf(-D[33], m, L[9]);
-      L[10] = fmaf(-D[35], m, L[10]);
-      L[11] = fmaf(-D[36], m, L[11]);
-      L[12] = fmaf(-D[38], m, L[12]);
-      L[13] = fmaf(-D[39], m, L[13]);
-      L[14] = fmaf(-D[41], m, L[14]);
-      L[15] = fmaf(-D[42], m, L[15]);
+    { const T m = __ldg(Mr + 6);
+      L[0] = m2l_fma(D[6], m, L[0]);
+      L[1] = m2l_fma(-D[12], m, L[1]);
+      L[2] = m2l_fma(-D[14], m, L[2]);
+      L[3] = m2l_fma(-D[15], m, L[3]);
+      L[4] = m2l_fma(D[21], m, L[4]);
+      L[5] = m2l_fma(D[23], m, L[5]);
+      L[6] = m2l_fma(D[24], m, L[6]);
+      L[7] = m2l_fma(D[26], m, L[7]);
+      L[8] = m2l_fma(D[27], m, L[8]);
+      L[9] = m2l_fma(-D[33], m, L[9]);
+      L[10] = m2l_fma(-D[35], m, L[10]);
+      L[11] = m2l_fma(-D[36], m, L[11]);
+      L[12] = m2l_fma(-D[38], m, L[12]);
+      L[13] = m2l_fma(-D[39], m, L[13]);
+      L[14] = m2l_fma(-D[41], m, L[14]);
+      L[15] = m2l_fma(-D[42], m, L[15]);
     }
-    { const float m = __ldg(Mr + 7);
-      L[0] = fmaf(D[7], m, L[0]);
-      L[1] = fmaf(-D[13], m, L[1]);
-      L[2] = fmaf(-D[16], m, L[2]);
-      L[3] = fmaf(-D[17], m, L[3]);
-      L[4] = fmaf(D[22], m, L[4]);
-      L[5] = fmaf(D[25], m, L[5]);
-      L[6] = fmaf(D[26], m, L[6]);
-      L[7] = fmaf(D[28], m, L[7]);
-      L[8] = fmaf(D[29], m, L[8]);
-      L[9] = fmaf(-D[34], m, L[9]);
-      L[10] = fmaf(-D[37], m, L[10]);
-      L[11] = fmaf(-D[38], m, L[11]);
-      L[12] = fmaf(-D[40], m, L[12]);
-      L[13] = fmaf(-D[41], m, L[13]);
-      L[14] = fmaf(-D[43], m, L[14]);
-      L[15] = fmaf(-D[44], m, L[15]);
+    { const T m = __ldg(Mr + 7);
+      L[0] = m2l_fma(D[7], m, L[0]);
+      L[1] = m2l_fma(-D[13], m, L[1]);
+      L[2] = m2l_fma(-D[16], m, L[2]);
+      L[3] = m2l_fma(-D[17], m, L[3]);
+      L[4] = m2l_fma(D[22], m, L[4]);
+      L[5] = m2l_fma(D[25], m, L[5]);
+      L[6] = m2l_fma(D[26], m, L[6]);
+      L[7] = m2l_fma(D[28], m, L[7]);
+      L[8] = m2l_fma(D[29], m, L[8]);
+      L[9] = m2l_fma(-D[34], m, L[9]);
+      L[10] = m2l_fma(-D[37], m, L[10]);
+      L[11] = m2l_fma(-D[38], m, L[11]);
+      L[12] = m2l_fma(-D[40], m, L[12]);
+      L[13] = m2l_fma(-D[41], m, L[13]);
+      L[14] = m2l_fma(-D[43], m, L[14]);
+      L[15] = m2l_fma(-D[44], m, L[15]);
     }
-    { const float m = __ldg(Mr + 8);
-      L[0] = fmaf(D[8], m, L[0]);
-      L[1] = fmaf(-D[14], m, L[1]);
-      L[2] = fmaf(-D[17], m, L[2]);
-      L[3] = fmaf(-D[18], m, L[3]);
-      L[4] = fmaf(D[23], m, L[4]);
-      L[5] = fmaf(D[26], m, L[5]);
-      L[6] = fmaf(D[27], m, L[6]);
-      L[7] = fmaf(D[29], m, L[7]);
-      L[8] = fmaf(D[30], m, L[8]);
-      L[9] = fmaf(-D[35], m, L[9]);
-      L[10] = fmaf(-D[38], m, L[10]);
-      L[11] = fmaf(-D[39], m, L[11]);
-      L[12] = fmaf(-D[41], m, L[12]);
-      L[13] = fmaf(-D[42], m, L[13]);
-      L[14] = fmaf(-D[44], m, L[14]);
-      L[15] = fmaf(-D[45], m, L[15]);
+    { const T m = __ldg(Mr + 8);
+      L[0] = m2l_fma(D[8], m, L[0]);
+      L[1] = m2l_fma(-D[14], m, L[1]);
+      L[2] = m2l_fma(-D[17], m, L[2]);
+      L[3] = m2l_fma(-D[18], m, L[3]);
+      L[4] = m2l_fma(D[23], m, L[4]);
+      L[5] = m2l_fma(D[26], m, L[5]);
+      L[6] = m2l_fma(D[27], m, L[6]);
+      L[7] = m2l_fma(D[29], m, L[7]);
+      L[8] = m2l_fma(D[30], m, L[8]);
+      L[9] = m2l_fma(-D[35], m, L[9]);
+      L[10] = m2l_fma(-D[38], m, L[10]);
+      L[11] = m2l_fma(-D[39], m, L[11]);
+      L[12] = m2l_fma(-D[41], m, L[12]);
+      L[13] = m2l_fma(-D[42], m, L[13]);
+      L[14] = m2l_fma(-D[44], m, L[14]);
+      L[15] = m2l_fma(-D[45], m, L[15]);
     }
-    { const float m = __ldg(Mr + 9);
-      L[0] = fmaf(D[10], m, L[0]);
-      L[1] = fmaf(-D[19], m, L[1]);
-      L[2] = fmaf(-D[20], m, L[2]);
-      L[3] = fmaf(-D[21], m, L[3]);
-      L[4] = fmaf(D[31], m, L[4]);
-      L[5] = fmaf(D[32], m, L[5]);
-      L[6] = fmaf(D[33], m, L[6]);
-      L[7] = fmaf(D[34], m, L[7]);
-      L[8] = fmaf(D[35], m, L[8]);
+    { const T m = __ldg(Mr + 9);
+      L[0] = m2l_fma(D[10], m, L[0]);
+      L[1] = m2l_fma(-D[19], m, L[1]);
+      L[2] = m2l_fma(-D[20], m, L[2]);
+      L[3] = m2l_fma(-D[21], m, L[3]);
+      L[4] = m2l_fma(D[31], m, L[4]);
+      L[5] = m2l_fma(D[32], m, L[5]);
+      L[6] = m2l_fma(D[33], m, L[6]);
+      L[7] = m2l_fma(D[34], m, L[7]);
+      L[8] = m2l_fma(D[35], m, L[8]);
     }
-    { const float m = __ldg(Mr + 10);
-      L[0] = fmaf(D[11], m, L[0]);
-      L[1] = fmaf(-D[20], m, L[1]);
-      L[2] = fmaf(-D[22], m, L[2]);
-      L[3] = fmaf(-D[23], m, L[3]);
-      L[4] = fmaf(D[32], m, L[4]);
-      L[5] = fmaf(D[34], m, L[5]);
-      L[6] = fmaf(D[35], m, L[6]);
-      L[7] = fmaf(D[37], m, L[7]);
-      L[8] = fmaf(D[38], m, L[8]);
+    { const T m = __ldg(Mr + 10);
+      L[0] = m2l_fma(D[11], m, L[0]);
+      L[1] = m2l_fma(-D[20], m, L[1]);
+      L[2] = m2l_fma(-D[22], m, L[2]);
+      L[3] = m2l_fma(-D[23], m, L[3]);
+      L[4] = m2l_fma(D[32], m, L[4]);
+      L[5] = m2l_fma(D[34], m, L[5]);
+      L[6] = m2l_fma(D[35], m, L[6]);
+      L[7] = m2l_fma(D[37], m, L[7]);
+      L[8] = m2l_fma(D[38], m, L[8]);
     }
-    { const float m = __ldg(Mr + 11);
-      L[0] = fmaf(D[12], m, L[0]);
-      L[1] = fmaf(-D[21], m, L[1]);
-      L[2] = fmaf(-D[23], m, L[2]);
-      L[3] = fmaf(-D[24], m, L[3]);
-      L[4] = fmaf(D[33], m, L[4]);
-      L[5] = fmaf(D[35], m, L[5]);
-      L[6] = fmaf(D[36], m, L[6]);
-      L[7] = fmaf(D[38], m, L[7]);
-      L[8] = fmaf(D[39], m, L[8]);
+    { const T m = __ldg(Mr + 11);
+      L[0] = m2l_fma(D[12], m, L[0]);
+      L[1] = m2l_fma(-D[21], m, L[1]);
+      L[2] = m2l_fma(-D[23], m, L[2]);
+      L[3] = m2l_fma(-D[24], m, L[3]);
+      L[4] = m2l_fma(D[33], m, L[4]);
+      L[5] = m2l_fma(D[35], m, L[5]);
+      L[6] = m2l_fma(D[36], m, L[6]);
+      L[7] = m2l_fma(D[38], m, L[7]);
+      L[8] = m2l_fma(D[39], m, L[8]);
     }
-    { const float m = __ldg(Mr + 12);
-      L[0] = fmaf(D[13], m, L[0]);
-      L[1] = fmaf(-D[22], m, L[1]);
-      L[2] = fmaf(-D[25], m, L[2]);
-      L[3] = fmaf(-D[26], m, L[3]);
-      L[4] = fmaf(D[34], m, L[4]);
-      L[5] = fmaf(D[37], m, L[5]);
-      L[6] = fmaf(D[38], m, L[6]);
-      L[7] = fmaf(D[40], m, L[7]);
-      L[8] = fmaf(D[41], m, L[8]);
+    { const T m = __ldg(Mr + 12);
+      L[0] = m2l_fma(D[13], m, L[0]);
+      L[1] = m2l_fma(-D[22], m, L[1]);
+      L[2] = m2l_fma(-D[25], m, L[2]);
+      L[3] = m2l_fma(-D[26], m, L[3]);
+      L[4] = m2l_fma(D[34], m, L[4]);
+      L[5] = m2l_fma(D[37], m, L[5]);
+      L[6] = m2l_fma(D[38], m, L[6]);
+      L[7] = m2l_fma(D[40], m, L[7]);
+      L[8] = m2l_fma(D[41], m, L[8]);
     }
-    { const float m = __ldg(Mr + 13);
-      L[0] = fmaf(D[14], m, L[0]);
-      L[1] = fmaf(-D[23], m, L[1]);
-      L[2] = fmaf(-D[26], m, L[2]);
-      L[3] = fmaf(-D[27], m, L[3]);
-      L[4] = fmaf(D[35], m, L[4]);
-      L[5] = fmaf(D[38], m, L[5]);
-      L[6] = fmaf(D[39], m, L[6]);
-      L[7] = fmaf(D[41], m, L[7]);
-      L[8] = fmaf(D[42], m, L[8]);
+    { const T m = __ldg(Mr + 13);
+      L[0] = m2l_fma(D[14], m, L[0]);
+      L[1] = m2l_fma(-D[23], m, L[1]);
+      L[2] = m2l_fma(-D[26], m, L[2]);
+      L[3] = m2l_fma(-D[27], m, L[3]);
+      L[4] = m2l_fma(D[35], m, L[4]);
+      L[5] = m2l_fma(D[38], m, L[5]);
+      L[6] = m2l_fma(D[39], m, L[6]);
+      L[7] = m2l_fma(D[41], m, L[7]);
+      L[8] = m2l_fma(D[42], m, L[8]);
     }
-    { const float m = __ldg(Mr + 14);
-      L[0] = fmaf(D[16], m, L[0]);
-      L[1] = fmaf(-D[25], m, L[1]);
-      L[2] = fmaf(-D[28], m, L[2]);
-      L[3] = fmaf(-D[29], m, L[3]);
-      L[4] = fmaf(D[37], m, L[4]);
-      L[5] = fmaf(D[40], m, L[5]);
-      L[6] = fmaf(D[41], m, L[6]);
-      L[7] = fmaf(D[43], m, L[7]);
-      L[8] = fmaf(D[44], m, L[8]);
+    { const T m = __ldg(Mr + 14);
+      L[0] = m2l_fma(D[16], m, L[0]);
+      L[1] = m2l_fma(-D[25], m, L[1]);
+      L[2] = m2l_fma(-D[28], m, L[2]);
+      L[3] = m2l_fma(-D[29], m, L[3]);
+      L[4] = m2l_fma(D[37], m, L[4]);
+      L[5] = m2l_fma(D[40], m, L[5]);
+      L[6] = m2l_fma(D[41], m, L[6]);
+      L[7] = m2l_fma(D[43], m, L[7]);
+      L[8] = m2l_fma(D[44], m, L[8]);
     }
-    { const float m = __ldg(Mr + 15);
-      L[0] = fmaf(D[17], m, L[0]);
-      L[1] = fmaf(-D[26], m, L[1]);
-      L[2] = fmaf(-D[29], m, L[2]);
-      L[3] = fmaf(-D[30], m, L[3]);
-      L[4] = fmaf(D[38], m, L[4]);
-      L[5] = fmaf(D[41], m, L[5]);
-      L[6] = fmaf(D[42], m, L[6]);
-      L[7] = fmaf(D[44], m, L[7]);
-      L[8] = fmaf(D[45], m, L[8]);
+    { const T m = __ldg(Mr + 15);
+      L[0] = m2l_fma(D[17], m, L[0]);
+      L[1] = m2l_fma(-D[26], m, L[1]);
+      L[2] = m2l_fma(-D[29], m, L[2]);
+      L[3] = m2l_fma(-D[30], m, L[3]);
+      L[4] = m2l_fma(D[38], m, L[4]);
+      L[5] = m2l_fma(D[41], m, L[5]);
+      L[6] = m2l_fma(D[42], m, L[6]);
+      L[7] = m2l_fma(D[44], m, L[7]);
+      L[8] = m2l_fma(D[45], m, L[8]);
     }
-    { const float m = __ldg(Mr + 16);
-      L[0] = fmaf(D[19], m, L[0]);
-      L[1] = fmaf(-D[31], m, L[1]);
-      L[2] = fmaf(-D[32], m, L[2]);
-      L[3] = fmaf(-D[33], m, L[3]);
+    { const T m = __ldg(Mr + 16);
+      L[0] = m2l_fma(D[19], m, L[0]);
+      L[1] = m2l_fma(-D[31], m, L[1]);
+      L[2] = m2l_fma(-D[32], m, L[2]);
+      L[3] = m2l_fma(-D[33], m, L[3]);
     }
-    { const float m = __ldg(Mr + 17);
-      L[0] = fmaf(D[20], m, L[0]);
-      L[1] = fmaf(-D[32], m, L[1]);
-      L[2] = fmaf(-D[34], m, L[2]);
-      L[3] = fmaf(-D[35], m, L[3]);
+    { const T m = __ldg(Mr + 17);
+      L[0] = m2l_fma(D[20], m, L[0]);
+      L[1] = m2l_fma(-D[32], m, L[1]);
+      L[2] = m2l_fma(-D[34], m, L[2]);
+      L[3] = m2l_fma(-D[35], m, L[3]);
     }
-    { const float m = __ldg(Mr + 18);
-      L[0] = fmaf(D[21], m, L[0]);
-      L[1] = fmaf(-D[33], m, L[1]);
-      L[2] = fmaf(-D[35], m, L[2]);
-      L[3] = fmaf(-D[36], m, L[3]);
+    { const T m = __ldg(Mr + 18);
+      L[0] = m2l_fma(D[21], m, L[0]);
+      L[1] = m2l_fma(-D[33], m, L[1]);
+      L[2] = m2l_fma(-D[35], m, L[2]);
+      L[3] = m2l_fma(-D[36], m, L[3]);
     }
-    { const float m = __ldg(Mr + 19);
-      L[0] = fmaf(D[22], m, L[0]);
-      L[1] = fmaf(-D[34], m, L[1]);
-      L[2] = fmaf(-D[37], m, L[2]);
-      L[3] = fmaf(-D[38], m, L[3]);
+    { const T m = __ldg(Mr + 19);
+      L[0] = m2l_fma(D[22], m, L[0]);
+      L[1] = m2l_fma(-D[34], m, L[1]);
+      L[2] = m2l_fma(-D[37], m, L[2]);
+      L[3] = m2l_fma(-D[38], m, L[3]);
     }
-    { const float m = __ldg(Mr + 20);
-      L[0] = fmaf(D[23], m, L[0]);
-      L[1] = fmaf(-D[35], m, L[1]);
-      L[2] = fmaf(-D[38], m, L[2]);
-      L[3] = fmaf(-D[39], m, L[3]);
+    { const T m = __ldg(Mr + 20);
+      L[0] = m2l_fma(D[23], m, L[0]);
+      L[1] = m2l_fma(-D[35], m, L[1]);
+      L[2] = m2l_fma(-D[38], m, L[2]);
+      L[3] = m2l_fma(-D[39], m, L[3]);
     }
-    { const float m = __ldg(Mr + 21);
-      L[0] = fmaf(D[25], m, L[0]);
-      L[1] = fmaf(-D[37], m, L[1]);
-      L[2] = fmaf(-D[40], m, L[2]);
-      L[3] = fmaf(-D[41], m, L[3]);
+    { const T m = __ldg(Mr + 21);
+      L[0] = m2l_fma(D[25], m, L[0]);
+      L[1] = m2l_fma(-D[37], m, L[1]);
+      L[2] = m2l_fma(-D[40], m, L[2]);
+      L[3] = m2l_fma(-D[41], m, L[3]);
     }
-    { const float m = __ldg(Mr + 22);
-      L[0] = fmaf(D[26], m, L[0]);
-      L[1] = fmaf(-D[38], m, L[1]);
-      L[2] = fmaf(-D[41], m, L[2]);
-      L[3] = fmaf(-D[42], m, L[3]);
+    { const T m = __ldg(Mr + 22);
+      L[0] = m2l_fma(D[26], m, L[0]);
+      L[1] = m2l_fma(-D[38], m, L[1]);
+      L[2] = m2l_fma(-D[41], m, L[2]);
+      L[3] = m2l_fma(-D[42], m, L[3]);
     }
-    { const float m = __ldg(Mr + 23);
-      L[0] = fmaf(D[28], m, L[0]);
-      L[1] = fmaf(-D[40], m, L[1]);
-      L[2] = fmaf(-D[43], m, L[2]);
-      L[3] = fmaf(-D[44], m, L[3]);
+    { const T m = __ldg(Mr + 23);
+      L[0] = m2l_fma(D[28], m, L[0]);
+      L[1] = m2l_fma(-D[40], m, L[1]);
+      L[2] = m2l_fma(-D[43], m, L[2]);
+      L[3] = m2l_fma(-D[44], m, L[3]);
     }
-    { const float m = __ldg(Mr + 24);
-      L[0] = fmaf(D[29], m, L[0]);
-      L[1] = fmaf(-D[41], m, L[1]);
-      L[2] = fmaf(-D[44], m, L[2]);
-      L[3] = fmaf(-D[45], m, L[3]);
+    { const T m = __ldg(Mr + 24);
+      L[0] = m2l_fma(D[29], m, L[0]);
+      L[1] = m2l_fma(-D[41], m, L[1]);
+      L[2] = m2l_fma(-D[44], m, L[2]);
+      L[3] = m2l_fma(-D[45], m, L[3]);
     }
-    { const float m = __ldg(Mr + 25);
-      L[0] = fmaf(D[31], m, L[0]);
+    { const T m = __ldg(Mr + 25);
+      L[0] = m2l_fma(D[31], m, L[0]);
     }
-    { const float m = __ldg(Mr + 26);
-      L[0] = fmaf(D[32], m, L[0]);
+    { const T m = __ldg(Mr + 26);
+      L[0] = m2l_fma(D[32], m, L[0]);
     }
-    { const float m = __ldg(Mr + 27);
-      L[0] = fmaf(D[33], m, L[0]);
+    { const T m = __ldg(Mr + 27);
+      L[0] = m2l_fma(D[33], m, L[0]);
     }
-    { const float m = __ldg(Mr + 28);
-      L[0] = fmaf(D[34], m, L[0]);
+    { const T m = __ldg(Mr + 28);
+      L[0] = m2l_fma(D[34], m, L[0]);
     }
-    { const float m = __ldg(Mr + 29);
-      L[0] = fmaf(D[35], m, L[0]);
+    { const T m = __ldg(Mr + 29);
+      L[0] = m2l_fma(D[35], m, L[0]);
     }
-    { const float m = __ldg(Mr + 30);
-      L[0] = fmaf(D[37], m, L[0]);
+    { const T m = __ldg(Mr + 30);
+      L[0] = m2l_fma(D[37], m, L[0]);
     }
-    { const float m = __ldg(Mr + 31);
-      L[0] = fmaf(D[38], m, L[0]);
+    { const T m = __ldg(Mr + 31);
+      L[0] = m2l_fma(D[38], m, L[0]);
     }
-    { const float m = __ldg(Mr + 32);
-      L[0] = fmaf(D[40], m, L[0]);
+    { const T m = __ldg(Mr + 32);
+      L[0] = m2l_fma(D[40], m, L[0]);
     }
-    { const float m = __ldg(Mr + 33);
-      L[0] = fmaf(D[41], m, L[0]);
+    { const T m = __ldg(Mr + 33);
+      L[0] = m2l_fma(D[41], m, L[0]);
     }
-    { const float m = __ldg(Mr + 34);
-      L[0] = fmaf(D[43], m, L[0]);
+    { const T m = __ldg(Mr + 34);
+      L[0] = m2l_fma(D[43], m, L[0]);
     }
-    { const float m = __ldg(Mr + 35);
-      L[0] = fmaf(D[44], m, L[0]);
+    { const T m = __ldg(Mr + 35);
+      L[0] = m2l_fma(D[44], m, L[0]);
     }
 }
 
-__device__ __forceinline__ void m2l_side_a_h_forces_5(const float (&D)[46], const float *__restrict__ Mr, float rho, float (&L)[36])
+template <class T> __device__ __forceinline__ void m2l_side_a_h_forces_5(const T (&D)[46], const T *__restrict__ Mr, T rho, T (&L)[36])
 {
-    L[0] = 0.0f;
-    float rp = 1.0f;
-    { const float m = __ldg(Mr + 0) * rp;
+    L[0] = T(0);
+    T rp = T(1);
+    { const T m = __ldg(Mr + 0) * rp;
       L[1] = D[1] * m;
       L[2] = D[2] * m;
       L[3] = D[3] * m;
@@ -12578,617 +12578,617 @@ __device__ __forceinline__ void m2l_side_a_h_forces_5(const float (&D)[46], cons
       L[35] = D[44] * m;
     }
     rp *= rho;
-    { const float m = -__ldg(Mr + 1) * rp;
-      L[1] = fmaf(D[4], m, L[1]);
-      L[2] = fmaf(D[5], m, L[2]);
-      L[3] = fmaf(D[6], m, L[3]);
-      L[4] = fmaf(D[10], m, L[4]);
-      L[5] = fmaf(D[11], m, L[5]);
-      L[6] = fmaf(D[12], m, L[6]);
-      L[7] = fmaf(D[13], m, L[7]);
-      L[8] = fmaf(D[14], m, L[8]);
-      L[9] = fmaf(D[19], m, L[9]);
-      L[10] = fmaf(D[20], m, L[10]);
-      L[11] = fmaf(D[21], m, L[11]);
-      L[12] = fmaf(D[22], m, L[12]);
-      L[13] = fmaf(D[23], m, L[13]);
-      L[14] = fmaf(D[25], m, L[14]);
-      L[15] = fmaf(D[26], m, L[15]);
-      L[16] = fmaf(D[31], m, L[16]);
-      L[17] = fmaf(D[32], m, L[17]);
-      L[18] = fmaf(D[33], m, L[18]);
-      L[19] = fmaf(D[34], m, L[19]);
-      L[20] = fmaf(D[35], m, L[20]);
-      L[21] = fmaf(D[37], m, L[21]);
-      L[22] = fmaf(D[38], m, L[22]);
-      L[23] = fmaf(D[40], m, L[23]);
-      L[24] = fmaf(D[41], m, L[24]);
+    { const T m = -__ldg(Mr + 1) * rp;
+      L[1] = m2l_fma(D[4], m, L[1]);
+      L[2] = m2l_fma(D[5], m, L[2]);
+      L[3] = m2l_fma(D[6], m, L[3]);
+      L[4] = m2l_fma(D[10], m, L[4]);
+      L[5] = m2l_fma(D[11], m, L[5]);
+      L[6] = m2l_fma(D[12], m, L[6]);
+      L[7] = m2l_fma(D[13], m, L[7]);
+      L[8] = m2l_fma(D[14], m, L[8]);
+      L[9] = m2l_fma(D[19], m, L[9]);
+      L[10] = m2l_fma(D[20], m, L[10]);
+      L[11] = m2l_fma(D[21], m, L[11]);
+      L[12] = m2l_fma(D[22], m, L[12]);
+      L[13] = m2l_fma(D[23], m, L[13]);
+      L[14] = m2l_fma(D[25], m, L[14]);
+      L[15] = m2l_fma(D[26], m, L[15]);
+      L[16] = m2l_fma(D[31], m, L[16]);
+      L[17] = m2l_fma(D[32], m, L[17]);
+      L[18] = m2l_fma(D[33], m, L[18]);
+      L[19] = m2l_fma(D[34], m, L[19]);
+      L[20] = m2l_fma(D[35], m, L[20]);
+      L[21] = m2l_fma(D[37], m, L[21]);
+      L[22] = m2l_fma(D[38], m, L[22]);
+      L[23] = m2l_fma(D[40], m, L[23]);
+      L[24] = m2l_fma(D[41], m, L[24]);
     }
-    { const float m = -__ldg(Mr + 2) * rp;
-      L[1] = fmaf(D[5], m, L[1]);
-      L[2] = fmaf(D[7], m, L[2]);
-      L[3] = fmaf(D[8], m, L[3]);
-      L[4] = fmaf(D[11], m, L[4]);
-      L[5] = fmaf(D[13], m, L[5]);
-      L[6] = fmaf(D[14], m, L[6]);
-      L[7] = fmaf(D[16], m, L[7]);
-      L[8] = fmaf(D[17], m, L[8]);
-      L[9] = fmaf(D[20], m, L[9]);
-      L[10] = fmaf(D[22], m, L[10]);
-      L[11] = fmaf(D[23], m, L[11]);
-      L[12] = fmaf(D[25], m, L[12]);
-      L[13] = fmaf(D[26], m, L[13]);
-      L[14] = fmaf(D[28], m, L[14]);
-      L[15] = fmaf(D[29], m, L[15]);
-      L[16] = fmaf(D[32], m, L[16]);
-      L[17] = fmaf(D[34], m, L[17]);
-      L[18] = fmaf(D[35], m, L[18]);
-      L[19] = fmaf(D[37], m, L[19]);
-      L[20] = fmaf(D[38], m, L[20]);
-      L[21] = fmaf(D[40], m, L[21]);
-      L[22] = fmaf(D[41], m, L[22]);
-      L[23] = fmaf(D[43], m, L[23]);
-      L[24] = fmaf(D[44], m, L[24]);
+    { const T m = -__ldg(Mr + 2) * rp;
+      L[1] = m2l_fma(D[5], m, L[1]);
+      L[2] = m2l_fma(D[7], m, L[2]);
+      L[3] = m2l_fma(D[8], m, L[3]);
+      L[4] = m2l_fma(D[11], m, L[4]);
+      L[5] = m2l_fma(D[13], m, L[5]);
+      L[6] = m2l_fma(D[14], m, L[6]);
+      L[7] = m2l_fma(D[16], m, L[7]);
+      L[8] = m2l_fma(D[17], m, L[8]);
+      L[9] = m2l_fma(D[20], m, L[9]);
+      L[10] = m2l_fma(D[22], m, L[10]);
+      L[11] = m2l_fma(D[23], m, L[11]);
+      L[12] = m2l_fma(D[25], m, L[12]);
+      L[13] = m2l_fma(D[26], m, L[13]);
+      L[14] = m2l_fma(D[28], m, L[14]);
+      L[15] = m2l_fma(D[29], m, L[15]);
+      L[16] = m2l_fma(D[32], m, L[16]);
+      L[17] = m2l_fma(D[34], m, L[17]);
+      L[18] = m2l_fma(D[35], m, L[18]);
+      L[19] = m2l_fma(D[37], m, L[19]);
+      L[20] = m2l_fma(D[38], m, L[20]);
+      L[21] = m2l_fma(D[40], m, L[21]);
+      L[22] = m2l_fma(D[41], m, L[22]);
+      L[23] = m2l_fma(D[43], m, L[23]);
+      L[24] = m2l_fma(D[44], m, L[24]);
     }
-    { const float m = -__ldg(Mr + 3) * rp;
-      L[1] = fmaf(D[6], m, L[1]);
-      L[2] = fmaf(D[8], m, L[2]);
-      L[3] = fmaf(D[9], m, L[3]);
-      L[4] = fmaf(D[12], m, L[4]);
-      L[5] = fmaf(D[14], m, L[5]);
-      L[6] = fmaf(D[15], m, L[6]);
-      L[7] = fmaf(D[17], m, L[7]);
-      L[8] = fmaf(D[18], m, L[8]);
-      L[9] = fmaf(D[21], m, L[9]);
-      L[10] = fmaf(D[23], m, L[10]);
-      L[11] = fmaf(D[24], m, L[11]);
-      L[12] = fmaf(D[26], m, L[12]);
-      L[13] = fmaf(D[27], m, L[13]);
-      L[14] = fmaf(D[29], m, L[14]);
-      L[15] = fmaf(D[30], m, L[15]);
-      L[16] = fmaf(D[33], m, L[16]);
-      L[17] = fmaf(D[35], m, L[17]);
-      L[18] = fmaf(D[36], m, L[18]);
-      L[19] = fmaf(D[38], m, L[19]);
-      L[20] = fmaf(D[39], m, L[20]);
-      L[21] = fmaf(D[41], m, L[21]);
-      L[22] = fmaf(D[42], m, L[22]);
-      L[23] = fmaf(D[44], m, L[23]);
-      L[24] = fmaf(D[45], m, L[24]);
-    }
-    rp *= rho;
-    { const float m = __ldg(Mr + 4) * rp;
-      L[1] = fmaf(D[10], m, L[1]);
-      L[2] = fmaf(D[11], m, L[2]);
-      L[3] = fmaf(D[12], m, L[3]);
-      L[4] = fmaf(D[19], m, L[4]);
-      L[5] = fmaf(D[20], m, L[5]);
-      L[6] = fmaf(D[21], m, L[6]);
-      L[7] = fmaf(D[22], m, L[7]);
-      L[8] = fmaf(D[23], m, L[8]);
-      L[9] = fmaf(D[31], m, L[9]);
-      L[10] = fmaf(D[32], m, L[10]);
-      L[11] = fmaf(D[33], m, L[11]);
-      L[12] = fmaf(D[34], m, L[12]);
-      L[13] = fmaf(D[35], m, L[13]);
-      L[14] = fmaf(D[37], m, L[14]);
-      L[15] = fmaf(D[38], m, L[15]);
-    }
-    { const float m = __ldg(Mr + 5) * rp;
-      L[1] = fmaf(D[11], m, L[1]);
-      L[2] = fmaf(D[13], m, L[2]);
-      L[3] = fmaf(D[14], m, L[3]);
-      L[4] = fmaf(D[20], m, L[4]);
-      L[5] = fmaf(D[22], m, L[5]);
-      L[6] = fmaf(D[23], m, L[6]);
-      L[7] = fmaf(D[25], m, L[7]);
-      L[8] = fmaf(D[26], m, L[8]);
-      L[9] = fmaf(D[32], m, L[9]);
-      L[10] = fmaf(D[34], m, L[10]);
-      L[11] = fmaf(D[35], m, L[11]);
-      L[12] = fmaf(D[37], m, L[12]);
-      L[13] = fmaf(D[38], m, L[13]);
-      L[14] = fmaf(D[40], m, L[14]);
-      L[15] = fmaf(D[41], m, L[15]);
-    }
-    { const float m = __ldg(Mr + 6) * rp;
-      L[1] = fmaf(D[12], m, L[1]);
-      L[2] = fmaf(D[14], m, L[2]);
-      L[3] = fmaf(D[15], m, L[3]);
-      L[4] = fmaf(D[21], m, L[4]);
-      L[5] = fmaf(D[23], m, L[5]);
-      L[6] = fmaf(D[24], m, L[6]);
-      L[7] = fmaf(D[26], m, L[7]);
-      L[8] = fmaf(D[27], m, L[8]);
-      L[9] = fmaf(D[33], m, L[9]);
-      L[10] = fmaf(D[35], m, L[10]);
-      L[11] = fmaf(D[36], m, L[11]);
-      L[12] = fmaf(D[38], m, L[12]);
-      L[13] = fmaf(D[39], m, L[13]);
-      L[14] = fmaf(D[41], m, L[14]);
-      L[15] = fmaf(D[42], m, L[15]);
-    }
-    { const float m = __ldg(Mr + 7) * rp;
-      L[1] = fmaf(D[13], m, L[1]);
-      L[2] = fmaf(D[16], m, L[2]);
-      L[3] = fmaf(D[17], m, L[3]);
-      L[4] = fmaf(D[22], m, L[4]);
-      L[5] = fmaf(D[25], m, L[5]);
-      L[6] = fmaf(D[26], m, L[6]);
-      L[7] = fmaf(D[28], m, L[7]);
-      L[8] = fmaf(D[29], m, L[8]);
-      L[9] = fmaf(D[34], m, L[9]);
-      L[10] = fmaf(D[37], m, L[10]);
-      L[11] = fmaf(D[38], m, L[11]);
-      L[12] = fmaf(D[40], m, L[12]);
-      L[13] = fmaf(D[41], m, L[13]);
-      L[14] = fmaf(D[43], m, L[14]);
-      L[15] = fmaf(D[44], m, L[15]);
-    }
-    { const float m = __ldg(Mr + 8) * rp;
-      L[1] = fmaf(D[14], m, L[1]);
-      L[2] = fmaf(D[17], m, L[2]);
-      L[3] = fmaf(D[18], m, L[3]);
-      L[4] = fmaf(D[23], m, L[4]);
-      L[5] = fmaf(D[26], m, L[5]);
-      L[6] = fmaf(D[27], m, L[6]);
-      L[7] = fmaf(D[29], m, L[7]);
-      L[8] = fmaf(D[30], m, L[8]);
-      L[9] = fmaf(D[35], m, L[9]);
-      L[10] = fmaf(D[38], m, L[10]);
-      L[11] = fmaf(D[39], m, L[11]);
-      L[12] = fmaf(D[41], m, L[12]);
-      L[13] = fmaf(D[42], m, L[13]);
-      L[14] = fmaf(D[44], m, L[14]);
-      L[15] = fmaf(D[45], m, L[15]);
+    { const T m = -__ldg(Mr + 3) * rp;
+      L[1] = m2l_fma(D[6], m, L[1]);
+      L[2] = m2l_fma(D[8], m, L[2]);
+      L[3] = m2l_fma(D[9], m, L[3]);
+      L[4] = m2l_fma(D[12], m, L[4]);
+      L[5] = m2l_fma(D[14], m, L[5]);
+      L[6] = m2l_fma(D[15], m, L[6]);
+      L[7] = m2l_fma(D[17], m, L[7]);
+      L[8] = m2l_fma(D[18], m, L[8]);
+      L[9] = m2l_fma(D[21], m, L[9]);
+      L[10] = m2l_fma(D[23], m, L[10]);
+      L[11] = m2l_fma(D[24], m, L[11]);
+      L[12] = m2l_fma(D[26], m, L[12]);
+      L[13] = m2l_fma(D[27], m, L[13]);
+      L[14] = m2l_fma(D[29], m, L[14]);
+      L[15] = m2l_fma(D[30], m, L[15]);
+      L[16] = m2l_fma(D[33], m, L[16]);
+      L[17] = m2l_fma(D[35], m, L[17]);
+      L[18] = m2l_fma(D[36], m, L[18]);
+      L[19] = m2l_fma(D[38], m, L[19]);
+      L[20] = m2l_fma(D[39], m, L[20]);
+      L[21] = m2l_fma(D[41], m, L[21]);
+      L[22] = m2l_fma(D[42], m, L[22]);
+      L[23] = m2l_fma(D[44], m, L[23]);
+      L[24] = m2l_fma(D[45], m, L[24]);
     }
     rp *= rho;
-    { const float m = -__ldg(Mr + 9) * rp;
-      L[1] = fmaf(D[19], m, L[1]);
-      L[2] = fmaf(D[20], m, L[2]);
-      L[3] = fmaf(D[21], m, L[3]);
-      L[4] = fmaf(D[31], m, L[4]);
-      L[5] = fmaf(D[32], m, L[5]);
-      L[6] = fmaf(D[33], m, L[6]);
-      L[7] = fmaf(D[34], m, L[7]);
-      L[8] = fmaf(D[35], m, L[8]);
+    { const T m = __ldg(Mr + 4) * rp;
+      L[1] = m2l_fma(D[10], m, L[1]);
+      L[2] = m2l_fma(D[11], m, L[2]);
+      L[3] = m2l_fma(D[12], m, L[3]);
+      L[4] = m2l_fma(D[19], m, L[4]);
+      L[5] = m2l_fma(D[20], m, L[5]);
+      L[6] = m2l_fma(D[21], m, L[6]);
+      L[7] = m2l_fma(D[22], m, L[7]);
+      L[8] = m2l_fma(D[23], m, L[8]);
+      L[9] = m2l_fma(D[31], m, L[9]);
+      L[10] = m2l_fma(D[32], m, L[10]);
+      L[11] = m2l_fma(D[33], m, L[11]);
+      L[12] = m2l_fma(D[34], m, L[12]);
+      L[13] = m2l_fma(D[35], m, L[13]);
+      L[14] = m2l_fma(D[37], m, L[14]);
+      L[15] = m2l_fma(D[38], m, L[15]);
     }
-    { const float m = -__ldg(Mr + 10) * rp;
-      L[1] = fmaf(D[20], m, L[1]);
-      L[2] = fmaf(D[22], m, L[2]);
-      L[3] = fmaf(D[23], m, L[3]);
-      L[4] = fmaf(D[32], m, L[4]);
-      L[5] = fmaf(D[34], m, L[5]);
-      L[6] = fmaf(D[35], m, L[6]);
-      L[7] = fmaf(D[37], m, L[7]);
-      L[8] = fmaf(D[38], m, L[8]);
+    { const T m = __ldg(Mr + 5) * rp;
+      L[1] = m2l_fma(D[11], m, L[1]);
+      L[2] = m2l_fma(D[13], m, L[2]);
+      L[3] = m2l_fma(D[14], m, L[3]);
+      L[4] = m2l_fma(D[20], m, L[4]);
+      L[5] = m2l_fma(D[22], m, L[5]);
+      L[6] = m2l_fma(D[23], m, L[6]);
+      L[7] = m2l_fma(D[25], m, L[7]);
+      L[8] = m2l_fma(D[26], m, L[8]);
+      L[9] = m2l_fma(D[32], m, L[9]);
+      L[10] = m2l_fma(D[34], m, L[10]);
+      L[11] = m2l_fma(D[35], m, L[11]);
+      L[12] = m2l_fma(D[37], m, L[12]);
+      L[13] = m2l_fma(D[38], m, L[13]);
+      L[14] = m2l_fma(D[40], m, L[14]);
+      L[15] = m2l_fma(D[41], m, L[15]);
     }
-    { const float m = -__ldg(Mr + 11) * rp;
-      L[1] = fmaf(D[21], m, L[1]);
-      L[2] = fmaf(D[23], m, L[2]);
-      L[3] = fmaf(D[24], m, L[3]);
-      L[4] = fmaf(D[33], m, L[4]);
-      L[5] = fmaf(D[35], m, L[5]);
-      L[6] = fmaf(D[36], m, L[6]);
-      L[7] = fmaf(D[38], m, L[7]);
-      L[8] = fmaf(D[39], m, L[8]);
+    { const T m = __ldg(Mr + 6) * rp;
+      L[1] = m2l_fma(D[12], m, L[1]);
+      L[2] = m2l_fma(D[14], m, L[2]);
+      L[3] = m2l_fma(D[15], m, L[3]);
+      L[4] = m2l_fma(D[21], m, L[4]);
+      L[5] = m2l_fma(D[23], m, L[5]);
+      L[6] = m2l_fma(D[24], m, L[6]);
+      L[7] = m2l_fma(D[26], m, L[7]);
+      L[8] = m2l_fma(D[27], m, L[8]);
+      L[9] = m2l_fma(D[33], m, L[9]);
+      L[10] = m2l_fma(D[35], m, L[10]);
+      L[11] = m2l_fma(D[36], m, L[11]);
+      L[12] = m2l_fma(D[38], m, L[12]);
+      L[13] = m2l_fma(D[39], m, L[13]);
+      L[14] = m2l_fma(D[41], m, L[14]);
+      L[15] = m2l_fma(D[42], m, L[15]);
     }
-    { const float m = -__ldg(Mr + 12) * rp;
-      L[1] = fmaf(D[22], m, L[1]);
-      L[2] = fmaf(D[25], m, L[2]);
-      L[3] = fmaf(D[26], m, L[3]);
-      L[4] = fmaf(D[34], m, L[4]);
-      L[5] = fmaf(D[37], m, L[5]);
-      L[6] = fmaf(D[38], m, L[6]);
-      L[7] = fmaf(D[40], m, L[7]);
-      L[8] = fmaf(D[41], m, L[8]);
+    { const T m = __ldg(Mr + 7) * rp;
+      L[1] = m2l_fma(D[13], m, L[1]);
+      L[2] = m2l_fma(D[16], m, L[2]);
+      L[3] = m2l_fma(D[17], m, L[3]);
+      L[4] = m2l_fma(D[22], m, L[4]);
+      L[5] = m2l_fma(D[25], m, L[5]);
+      L[6] = m2l_fma(D[26], m, L[6]);
+      L[7] = m2l_fma(D[28], m, L[7]);
+      L[8] = m2l_fma(D[29], m, L[8]);
+      L[9] = m2l_fma(D[34], m, L[9]);
+      L[10] = m2l_fma(D[37], m, L[10]);
+      L[11] = m2l_fma(D[38], m, L[11]);
+      L[12] = m2l_fma(D[40], m, L[12]);
+      L[13] = m2l_fma(D[41], m, L[13]);
+      L[14] = m2l_fma(D[43], m, L[14]);
+      L[15] = m2l_fma(D[44], m, L[15]);
     }
-    { const float m = -__ldg(Mr + 13) * rp;
-      L[1] = fmaf(D[23], m, L[1]);
-      L[2] = fmaf(D[26], m, L[2]);
-      L[3] = fmaf(D[27], m, L[3]);
-      L[4] = fmaf(D[35], m, L[4]);
-      L[5] = fmaf(D[38], m, L[5]);
-      L[6] = fmaf(D[39], m, L[6]);
-      L[7] = fmaf(D[41], m, L[7]);
-      L[8] = fmaf(D[42], m, L[8]);
-    }
-    { const float m = -__ldg(Mr + 14) * rp;
-      L[1] = fmaf(D[25], m, L[1]);
-      L[2] = fmaf(D[28], m, L[2]);
-      L[3] = fmaf(D[29], m, L[3]);
-      L[4] = fmaf(D[37], m, L[4]);
-      L[5] = fmaf(D[40], m, L[5]);
-      L[6] = fmaf(D[41], m, L[6]);
-      L[7] = fmaf(D[43], m, L[7]);
-      L[8] = fmaf(D[44], m, L[8]);
-    }
-    { const float m = -__ldg(Mr + 15) * rp;
-      L[1] = fmaf(D[26], m, L[1]);
-      L[2] = fmaf(D[29], m, L[2]);
-      L[3] = fmaf(D[30], m, L[3]);
-      L[4] = fmaf(D[38], m, L[4]);
-      L[5] = fmaf(D[41], m, L[5]);
-      L[6] = fmaf(D[42], m, L[6]);
-      L[7] = fmaf(D[44], m, L[7]);
-      L[8] = fmaf(D[45], m, L[8]);
+    { const T m = __ldg(Mr + 8) * rp;
+      L[1] = m2l_fma(D[14], m, L[1]);
+      L[2] = m2l_fma(D[17], m, L[2]);
+      L[3] = m2l_fma(D[18], m, L[3]);
+      L[4] = m2l_fma(D[23], m, L[4]);
+      L[5] = m2l_fma(D[26], m, L[5]);
+      L[6] = m2l_fma(D[27], m, L[6]);
+      L[7] = m2l_fma(D[29], m, L[7]);
+      L[8] = m2l_fma(D[30], m, L[8]);
+      L[9] = m2l_fma(D[35], m, L[9]);
+      L[10] = m2l_fma(D[38], m, L[10]);
+      L[11] = m2l_fma(D[39], m, L[11]);
+      L[12] = m2l_fma(D[41], m, L[12]);
+      L[13] = m2l_fma(D[42], m, L[13]);
+      L[14] = m2l_fma(D[44], m, L[14]);
+      L[15] = m2l_fma(D[45], m, L[15]);
     }
     rp *= rho;
-    { const float m = __ldg(Mr + 16) * rp;
-      L[1] = fmaf(D[31], m, L[1]);
-      L[2] = fmaf(D[32], m, L[2]);
-      L[3] = fmaf(D[33], m, L[3]);
+    { const T m = -__ldg(Mr + 9) * rp;
+      L[1] = m2l_fma(D[19], m, L[1]);
+      L[2] = m2l_fma(D[20], m, L[2]);
+      L[3] = m2l_fma(D[21], m, L[3]);
+      L[4] = m2l_fma(D[31], m, L[4]);
+      L[5] = m2l_fma(D[32], m, L[5]);
+      L[6] = m2l_fma(D[33], m, L[6]);
+      L[7] = m2l_fma(D[34], m, L[7]);
+      L[8] = m2l_fma(D[35], m, L[8]);
     }
-    { const float m = __ldg(Mr + 17) * rp;
-      L[1] = fmaf(D[32], m, L[1]);
-      L[2] = fmaf(D[34], m, L[2]);
-      L[3] = fmaf(D[35], m, L[3]);
+    { const T m = -__ldg(Mr + 10) * rp;
+      L[1] = m2l_fma(D[20], m, L[1]);
+      L[2] = m2l_fma(D[22], m, L[2]);
+      L[3] = m2l_fma(D[23], m, L[3]);
+      L[4] = m2l_fma(D[32], m, L[4]);
+      L[5] = m2l_fma(D[34], m, L[5]);
+      L[6] = m2l_fma(D[35], m, L[6]);
+      L[7] = m2l_fma(D[37], m, L[7]);
+      L[8] = m2l_fma(D[38], m, L[8]);
     }
-    { const float m = __ldg(Mr + 18) * rp;
-      L[1] = fmaf(D[33], m, L[1]);
-      L[2] = fmaf(D[35], m, L[2]);
-      L[3] = fmaf(D[36], m, L[3]);
+    { const T m = -__ldg(Mr + 11) * rp;
+      L[1] = m2l_fma(D[21], m, L[1]);
+      L[2] = m2l_fma(D[23], m, L[2]);
+      L[3] = m2l_fma(D[24], m, L[3]);
+      L[4] = m2l_fma(D[33], m, L[4]);
+      L[5] = m2l_fma(D[35], m, L[5]);
+      L[6] = m2l_fma(D[36], m, L[6]);
+      L[7] = m2l_fma(D[38], m, L[7]);
+      L[8] = m2l_fma(D[39], m, L[8]);
     }
-    { const float m = __ldg(Mr + 19) * rp;
-      L[1] = fmaf(D[34], m, L[1]);
-      L[2] = fmaf(D[37], m, L[2]);
-      L[3] = fmaf(D[38], m, L[3]);
+    { const T m = -__ldg(Mr + 12) * rp;
+      L[1] = m2l_fma(D[22], m, L[1]);
+      L[2] = m2l_fma(D[25], m, L[2]);
+      L[3] = m2l_fma(D[26], m, L[3]);
+      L[4] = m2l_fma(D[34], m, L[4]);
+      L[5] = m2l_fma(D[37], m, L[5]);
+      L[6] = m2l_fma(D[38], m, L[6]);
+      L[7] = m2l_fma(D[40], m, L[7]);
+      L[8] = m2l_fma(D[41], m, L[8]);
     }
-    { const float m = __ldg(Mr + 20) * rp;
-      L[1] = fmaf(D[35], m, L[1]);
-      L[2] = fmaf(D[38], m, L[2]);
-      L[3] = fmaf(D[39], m, L[3]);
+    { const T m = -__ldg(Mr + 13) * rp;
+      L[1] = m2l_fma(D[23], m, L[1]);
+      L[2] = m2l_fma(D[26], m, L[2]);
+      L[3] = m2l_fma(D[27], m, L[3]);
+      L[4] = m2l_fma(D[35], m, L[4]);
+      L[5] = m2l_fma(D[38], m, L[5]);
+      L[6] = m2l_fma(D[39], m, L[6]);
+      L[7] = m2l_fma(D[41], m, L[7]);
+      L[8] = m2l_fma(D[42], m, L[8]);
     }
-    { const float m = __ldg(Mr + 21) * rp;
-      L[1] = fmaf(D[37], m, L[1]);
-      L[2] = fmaf(D[40], m, L[2]);
-      L[3] = fmaf(D[41], m, L[3]);
+    { const T m = -__ldg(Mr + 14) * rp;
+      L[1] = m2l_fma(D[25], m, L[1]);
+      L[2] = m2l_fma(D[28], m, L[2]);
+      L[3] = m2l_fma(D[29], m, L[3]);
+      L[4] = m2l_fma(D[37], m, L[4]);
+      L[5] = m2l_fma(D[40], m, L[5]);
+      L[6] = m2l_fma(D[41], m, L[6]);
+      L[7] = m2l_fma(D[43], m, L[7]);
+      L[8] = m2l_fma(D[44], m, L[8]);
     }
-    { const float m = __ldg(Mr + 22) * rp;
-      L[1] = fmaf(D[38], m, L[1]);
-      L[2] = fmaf(D[41], m, L[2]);
-      L[3] = fmaf(D[42], m, L[3]);
+    { const T m = -__ldg(Mr + 15) * rp;
+      L[1] = m2l_fma(D[26], m, L[1]);
+      L[2] = m2l_fma(D[29], m, L[2]);
+      L[3] = m2l_fma(D[30], m, L[3]);
+      L[4] = m2l_fma(D[38], m, L[4]);
+      L[5] = m2l_fma(D[41], m, L[5]);
+      L[6] = m2l_fma(D[42], m, L[6]);
+      L[7] = m2l_fma(D[44], m, L[7]);
+      L[8] = m2l_fma(D[45], m, L[8]);
     }
-    { const float m = __ldg(Mr + 23) * rp;
-      L[1] = fmaf(D[40], m, L[1]);
-      L[2] = fmaf(D[43], m, L[2]);
-      L[3] = fmaf(D[44], m, L[3]);
+    rp *= rho;
+    { const T m = __ldg(Mr + 16) * rp;
+      L[1] = m2l_fma(D[31], m, L[1]);
+      L[2] = m2l_fma(D[32], m, L[2]);
+      L[3] = m2l_fma(D[33], m, L[3]);
     }
-    { const float m = __ldg(Mr + 24) * rp;
-      L[1] = fmaf(D[41], m, L[1]);
-      L[2] = fmaf(D[44], m, L[2]);
-      L[3] = fmaf(D[45], m, L[3]);
+    { const T m = __ldg(Mr + 17) * rp;
+      L[1] = m2l_fma(D[32], m, L[1]);
+      L[2] = m2l_fma(D[34], m, L[2]);
+      L[3] = m2l_fma(D[35], m, L[3]);
+    }
+    { const T m = __ldg(Mr + 18) * rp;
+      L[1] = m2l_fma(D[33], m, L[1]);
+      L[2] = m2l_fma(D[35], m, L[2]);
+      L[3] = m2l_fma(D[36], m, L[3]);
+    }
+    { const T m = __ldg(Mr + 19) * rp;
+      L[1] = m2l_fma(D[34], m, L[1]);
+      L[2] = m2l_fma(D[37], m, L[2]);
+      L[3] = m2l_fma(D[38], m, L[3]);
+    }
+    { const T m = __ldg(Mr + 20) * rp;
+      L[1] = m2l_fma(D[35], m, L[1]);
+      L[2] = m2l_fma(D[38], m, L[2]);
+      L[3] = m2l_fma(D[39], m, L[3]);
+    }
+    { const T m = __ldg(Mr + 21) * rp;
+      L[1] = m2l_fma(D[37], m, L[1]);
+      L[2] = m2l_fma(D[40], m, L[2]);
+      L[3] = m2l_fma(D[41], m, L[3]);
+    }
+    { const T m = __ldg(Mr + 22) * rp;
+      L[1] = m2l_fma(D[38], m, L[1]);
+      L[2] = m2l_fma(D[41], m, L[2]);
+      L[3] = m2l_fma(D[42], m, L[3]);
+    }
+    { const T m = __ldg(Mr + 23) * rp;
+      L[1] = m2l_fma(D[40], m, L[1]);
+      L[2] = m2l_fma(D[43], m, L[2]);
+      L[3] = m2l_fma(D[44], m, L[3]);
+    }
+    { const T m = __ldg(Mr + 24) * rp;
+      L[1] = m2l_fma(D[41], m, L[1]);
+      L[2] = m2l_fma(D[44], m, L[2]);
+      L[3] = m2l_fma(D[45], m, L[3]);
     }
 }
 
-__device__ __forceinline__ void m2l_acc_h_forces_5(const float (&D)[46], const float *__restrict__ Mr, float rho, float (&L)[36])
+template <class T> __device__ __forceinline__ void m2l_acc_h_forces_5(const T (&D)[46], const T *__restrict__ Mr, T rho, T (&L)[36])
 {
-    float rp = 1.0f;
-    { const float m = __ldg(Mr + 0) * rp;
-      L[1] = fmaf(D[1], m, L[1]);
-      L[2] = fmaf(D[2], m, L[2]);
-      L[3] = fmaf(D[3], m, L[3]);
-      L[4] = fmaf(D[4], m, L[4]);
-      L[5] = fmaf(D[5], m, L[5]);
-      L[6] = fmaf(D[6], m, L[6]);
-      L[7] = fmaf(D[7], m, L[7]);
-      L[8] = fmaf(D[8], m, L[8]);
-      L[9] = fmaf(D[10], m, L[9]);
-      L[10] = fmaf(D[11], m, L[10]);
-      L[11] = fmaf(D[12], m, L[11]);
-      L[12] = fmaf(D[13], m, L[12]);
-      L[13] = fmaf(D[14], m, L[13]);
-      L[14] = fmaf(D[16], m, L[14]);
-      L[15] = fmaf(D[17], m, L[15]);
-      L[16] = fmaf(D[19], m, L[16]);
-      L[17] = fmaf(D[20], m, L[17]);
-      L[18] = fmaf(D[21], m, L[18]);
-      L[19] = fmaf(D[22], m, L[19]);
-      L[20] = fmaf(D[23], m, L[20]);
-      L[21] = fmaf(D[25], m, L[21]);
-      L[22] = fmaf(D[26], m, L[22]);
-      L[23] = fmaf(D[28], m, L[23]);
-      L[24] = fmaf(D[29], m, L[24]);
-      L[25] = fmaf(D[31], m, L[25]);
-      L[26] = fmaf(D[32], m, L[26]);
-      L[27] = fmaf(D[33], m, L[27]);
-      L[28] = fmaf(D[34], m, L[28]);
-      L[29] = fmaf(D[35], m, L[29]);
-      L[30] = fmaf(D[37], m, L[30]);
-      L[31] = fmaf(D[38], m, L[31]);
-      L[32] = fmaf(D[40], m, L[32]);
-      L[33] = fmaf(D[41], m, L[33]);
-      L[34] = fmaf(D[43], m, L[34]);
-      L[35] = fmaf(D[44], m, L[35]);
+    T rp = T(1);
+    { const T m = __ldg(Mr + 0) * rp;
+      L[1] = m2l_fma(D[1], m, L[1]);
+      L[2] = m2l_fma(D[2], m, L[2]);
+      L[3] = m2l_fma(D[3], m, L[3]);
+      L[4] = m2l_fma(D[4], m, L[4]);
+      L[5] = m2l_fma(D[5], m, L[5]);
+      L[6] = m2l_fma(D[6], m, L[6]);
+      L[7] = m2l_fma(D[7], m, L[7]);
+      L[8] = m2l_fma(D[8], m, L[8]);
+      L[9] = m2l_fma(D[10], m, L[9]);
+      L[10] = m2l_fma(D[11], m, L[10]);
+      L[11] = m2l_fma(D[12], m, L[11]);
+      L[12] = m2l_fma(D[13], m, L[12]);
+      L[13] = m2l_fma(D[14], m, L[13]);
+      L[14] = m2l_fma(D[16], m, L[14]);
+      L[15] = m2l_fma(D[17], m, L[15]);
+      L[16] = m2l_fma(D[19], m, L[16]);
+      L[17] = m2l_fma(D[20], m, L[17]);
+      L[18] = m2l_fma(D[21], m, L[18]);
+      L[19] = m2l_fma(D[22], m, L[19]);
+      L[20] = m2l_fma(D[23], m, L[20]);
+      L[21] = m2l_fma(D[25], m, L[21]);
+      L[22] = m2l_fma(D[26], m, L[22]);
+      L[23] = m2l_fma(D[28], m, L[23]);
+      L[24] = m2l_fma(D[29], m, L[24]);
+      L[25] = m2l_fma(D[31], m, L[25]);
+      L[26] = m2l_fma(D[32], m, L[26]);
+      L[27] = m2l_fma(D[33], m, L[27]);
+      L[28] = m2l_fma(D[34], m, L[28]);
+      L[29] = m2l_fma(D[35], m, L[29]);
+      L[30] = m2l_fma(D[37], m, L[30]);
+      L[31] = m2l_fma(D[38], m, L[31]);
+      L[32] = m2l_fma(D[40], m, L[32]);
+      L[33] = m2l_fma(D[41], m, L[33]);
+      L[34] = m2l_fma(D[43], m, L[34]);
+      L[35] = m2l_fma(D[44], m, L[35]);
     }
     rp *= rho;
-    { const float m = -__ldg(Mr + 1) * rp;
-      L[1] = fmaf(D[4], m, L[1]);
-      L[2] = fmaf(D[5], m, L[2]);
-      L[3] = fmaf(D[6], m, L[3]);
-      L[4] = fmaf(D[10], m, L[4]);
-      L[5] = fmaf(D[11], m, L[5]);
-      L[6] = fmaf(D[12], m, L[6]);
-      L[7] = fmaf(D[13], m, L[7]);
-      L[8] = fmaf(D[14], m, L[8]);
-      L[9] = fmaf(D[19], m, L[9]);
-      L[10] = fmaf(D[20], m, L[10]);
-      L[11] = fmaf(D[21], m, L[11]);
-      L[12] = fmaf(D[22], m, L[12]);
-      L[13] = fmaf(D[23], m, L[13]);
-      L[14] = fmaf(D[25], m, L[14]);
-      L[15] = fmaf(D[26], m, L[15]);
-      L[16] = fmaf(D[31], m, L[16]);
-      L[17] = fmaf(D[32], m, L[17]);
-      L[18] = fmaf(D[33], m, L[18]);
-      L[19] = fmaf(D[34], m, L[19]);
-      L[20] = fmaf(D[35], m, L[20]);
-      L[21] = fmaf(D[37], m, L[21]);
-      L[22] = fmaf(D[38], m, L[22]);
-      L[23] = fmaf(D[40], m, L[23]);
-      L[24] = fmaf(D[41], m, L[24]);
+    { const T m = -__ldg(Mr + 1) * rp;
+      L[1] = m2l_fma(D[4], m, L[1]);
+      L[2] = m2l_fma(D[5], m, L[2]);
+      L[3] = m2l_fma(D[6], m, L[3]);
+      L[4] = m2l_fma(D[10], m, L[4]);
+      L[5] = m2l_fma(D[11], m, L[5]);
+      L[6] = m2l_fma(D[12], m, L[6]);
+      L[7] = m2l_fma(D[13], m, L[7]);
+      L[8] = m2l_fma(D[14], m, L[8]);
+      L[9] = m2l_fma(D[19], m, L[9]);
+      L[10] = m2l_fma(D[20], m, L[10]);
+      L[11] = m2l_fma(D[21], m, L[11]);
+      L[12] = m2l_fma(D[22], m, L[12]);
+      L[13] = m2l_fma(D[23], m, L[13]);
+      L[14] = m2l_fma(D[25], m, L[14]);
+      L[15] = m2l_fma(D[26], m, L[15]);
+      L[16] = m2l_fma(D[31], m, L[16]);
+      L[17] = m2l_fma(D[32], m, L[17]);
+      L[18] = m2l_fma(D[33], m, L[18]);
+      L[19] = m2l_fma(D[34], m, L[19]);
+      L[20] = m2l_fma(D[35], m, L[20]);
+      L[21] = m2l_fma(D[37], m, L[21]);
+      L[22] = m2l_fma(D[38], m, L[22]);
+      L[23] = m2l_fma(D[40], m, L[23]);
+      L[24] = m2l_fma(D[41], m, L[24]);
     }
-    { const float m = -__ldg(Mr + 2) * rp;
-      L[1] = fmaf(D[5], m, L[1]);
-      L[2] = fmaf(D[7], m, L[2]);
-      L[3] = fmaf(D[8], m, L[3]);
-      L[4] = fmaf(D[11], m, L[4]);
-      L[5] = fmaf(D[13], m, L[5]);
-      L[6] = fmaf(D[14], m, L[6]);
-      L[7] = fmaf(D[16], m, L[7]);
-      L[8] = fmaf(D[17], m, L[8]);
-      L[9] = fmaf(D[20], m, L[9]);
-      L[10] = fmaf(D[22], m, L[10]);
-      L[11] = fmaf(D[23], m, L[11]);
-      L[12] = fmaf(D[25], m, L[12]);
-      L[13] = fmaf(D[26], m, L[13]);
-      L[14] = fmaf(D[28], m, L[14]);
-      L[15] = fmaf(D[29], m, L[15]);
-      L[16] = fmaf(D[32], m, L[16]);
-      L[17] = fmaf(D[34], m, L[17]);
-      L[18] = fmaf(D[35], m, L[18]);
-      L[19] = fmaf(D[37], m, L[19]);
-      L[20] = fmaf(D[38], m, L[20]);
-      L[21] = fmaf(D[40], m, L[21]);
-      L[22] = fmaf(D[41], m, L[22]);
-      L[23] = fmaf(D[43], m, L[23]);
-      L[24] = fmaf(D[44], m, L[24]);
+    { const T m = -__ldg(Mr + 2) * rp;
+      L[1] = m2l_fma(D[5], m, L[1]);
+      L[2] = m2l_fma(D[7], m, L[2]);
+      L[3] = m2l_fma(D[8], m, L[3]);
+      L[4] = m2l_fma(D[11], m, L[4]);
+      L[5] = m2l_fma(D[13], m, L[5]);
+      L[6] = m2l_fma(D[14], m, L[6]);
+      L[7] = m2l_fma(D[16], m, L[7]);
+      L[8] = m2l_fma(D[17], m, L[8]);
+      L[9] = m2l_fma(D[20], m, L[9]);
+      L[10] = m2l_fma(D[22], m, L[10]);
+      L[11] = m2l_fma(D[23], m, L[11]);
+      L[12] = m2l_fma(D[25], m, L[12]);
+      L[13] = m2l_fma(D[26], m, L[13]);
+      L[14] = m2l_fma(D[28], m, L[14]);
+      L[15] = m2l_fma(D[29], m, L[15]);
+      L[16] = m2l_fma(D[32], m, L[16]);
+      L[17] = m2l_fma(D[34], m, L[17]);
+      L[18] = m2l_fma(D[35], m, L[18]);
+      L[19] = m2l_fma(D[37], m, L[19]);
+      L[20] = m2l_fma(D[38], m, L[20]);
+      L[21] = m2l_fma(D[40], m, L[21]);
+      L[22] = m2l_fma(D[41], m, L[22]);
+      L[23] = m2l_fma(D[43], m, L[23]);
+      L[24] = m2l_fma(D[44], m, L[24]);
     }
-    { const float m = -__ldg(Mr + 3) * rp;
-      L[1] = fmaf(D[6], m, L[1]);
-      L[2] = fmaf(D[8], m, L[2]);
-      L[3] = fmaf(D[9], m, L[3]);
-      L[4] = fmaf(D[12], m, L[4]);
-      L[5] = fmaf(D[14], m, L[5]);
-      L[6] = fmaf(D[15], m, L[6]);
-      L[7] = fmaf(D[17], m, L[7]);
-      L[8] = fmaf(D[18], m, L[8]);
-      L[9] = fmaf(D[21], m, L[9]);
-      L[10] = fmaf(D[23], m, L[10]);
-      L[11] = fmaf(D[24], m, L[11]);
-      L[12] = fmaf(D[26], m, L[12]);
-      L[13] = fmaf(D[27], m, L[13]);
-      L[14] = fmaf(D[29], m, L[14]);
-      L[15] = fmaf(D[30], m, L[15]);
-      L[16] = fmaf(D[33], m, L[16]);
-      L[17] = fmaf(D[35], m, L[17]);
-      L[18] = fmaf(D[36], m, L[18]);
-      L[19] = fmaf(D[38], m, L[19]);
-      L[20] = fmaf(D[39], m, L[20]);
-      L[21] = fmaf(D[41], m, L[21]);
-      L[22] = fmaf(D[42], m, L[22]);
-      L[23] = fmaf(D[44], m, L[23]);
-      L[24] = fmaf(D[45], m, L[24]);
-    }
-    rp *= rho;
-    { const float m = __ldg(Mr + 4) * rp;
-      L[1] = fmaf(D[10], m, L[1]);
-      L[2] = fmaf(D[11], m, L[2]);
-      L[3] = fmaf(D[12], m, L[3]);
-      L[4] = fmaf(D[19], m, L[4]);
-      L[5] = fmaf(D[20], m, L[5]);
-      L[6] = fmaf(D[21], m, L[6]);
-      L[7] = fmaf(D[22], m, L[7]);
-      L[8] = fmaf(D[23], m, L[8]);
-      L[9] = fmaf(D[31], m, L[9]);
-      L[10] = fmaf(D[32], m, L[10]);
-      L[11] = fmaf(D[33], m, L[11]);
-      L[12] = fmaf(D[34], m, L[12]);
-      L[13] = fmaf(D[35], m, L[13]);
-      L[14] = fmaf(D[37], m, L[14]);
-      L[15] = fmaf(D[38], m, L[15]);
-    }
-    { const float m = __ldg(Mr + 5) * rp;
-      L[1] = fmaf(D[11], m, L[1]);
-      L[2] = fmaf(D[13], m, L[2]);
-      L[3] = fmaf(D[14], m, L[3]);
-      L[4] = fmaf(D[20], m, L[4]);
-      L[5] = fmaf(D[22], m, L[5]);
-      L[6] = fmaf(D[23], m, L[6]);
-      L[7] = fmaf(D[25], m, L[7]);
-      L[8] = fmaf(D[26], m, L[8]);
-      L[9] = fmaf(D[32], m, L[9]);
-      L[10] = fmaf(D[34], m, L[10]);
-      L[11] = fmaf(D[35], m, L[11]);
-      L[12] = fmaf(D[37], m, L[12]);
-      L[13] = fmaf(D[38], m, L[13]);
-      L[14] = fmaf(D[40], m, L[14]);
-      L[15] = fmaf(D[41], m, L[15]);
-    }
-    { const float m = __ldg(Mr + 6) * rp;
-      L[1] = fmaf(D[12], m, L[1]);
-      L[2] = fmaf(D[14], m, L[2]);
-      L[3] = fmaf(D[15], m, L[3]);
-      L[4] = fmaf(D[21], m, L[4]);
-      L[5] = fmaf(D[23], m, L[5]);
-      L[6] = fmaf(D[24], m, L[6]);
-      L[7] = fmaf(D[26], m, L[7]);
-      L[8] = fmaf(D[27], m, L[8]);
-      L[9] = fmaf(D[33], m, L[9]);
-      L[10] = fmaf(D[35], m, L[10]);
-      L[11] = fmaf(D[36], m, L[11]);
-      L[12] = fmaf(D[38], m, L[12]);
-      L[13] = fmaf(D[39], m, L[13]);
-      L[14] = fmaf(D[41], m, L[14]);
-      L[15] = fmaf(D[42], m, L[15]);
-    }
-    { const float m = __ldg(Mr + 7) * rp;
-      L[1] = fmaf(D[13], m, L[1]);
-      L[2] = fmaf(D[16], m, L[2]);
-      L[3] = fmaf(D[17], m, L[3]);
-      L[4] = fmaf(D[22], m, L[4]);
-      L[5] = fmaf(D[25], m, L[5]);
-      L[6] = fmaf(D[26], m, L[6]);
-      L[7] = fmaf(D[28], m, L[7]);
-      L[8] = fmaf(D[29], m, L[8]);
-      L[9] = fmaf(D[34], m, L[9]);
-      L[10] = fmaf(D[37], m, L[10]);
-      L[11] = fmaf(D[38], m, L[11]);
-      L[12] = fmaf(D[40], m, L[12]);
-      L[13] = fmaf(D[41], m, L[13]);
-      L[14] = fmaf(D[43], m, L[14]);
-      L[15] = fmaf(D[44], m, L[15]);
-    }
-    { const float m = __ldg(Mr + 8) * rp;
-      L[1] = fmaf(D[14], m, L[1]);
-      L[2] = fmaf(D[17], m, L[2]);
-      L[3] = fmaf(D[18], m, L[3]);
-      L[4] = fmaf(D[23], m, L[4]);
-      L[5] = fmaf(D[26], m, L[5]);
-      L[6] = fmaf(D[27], m, L[6]);
-      L[7] = fmaf(D[29], m, L[7]);
-      L[8] = fmaf(D[30], m, L[8]);
-      L[9] = fmaf(D[35], m, L[9]);
-      L[10] = fmaf(D[38], m, L[10]);
-      L[11] = fmaf(D[39], m, L[11]);
-      L[12] = fmaf(D[41], m, L[12]);
-      L[13] = fmaf(D[42], m, L[13]);
-      L[14] = fmaf(D[44], m, L[14]);
-      L[15] = fmaf(D[45], m, L[15]);
+    { const T m = -__ldg(Mr + 3) * rp;
+      L[1] = m2l_fma(D[6], m, L[1]);
+      L[2] = m2l_fma(D[8], m, L[2]);
+      L[3] = m2l_fma(D[9], m, L[3]);
+      L[4] = m2l_fma(D[12], m, L[4]);
+      L[5] = m2l_fma(D[14], m, L[5]);
+      L[6] = m2l_fma(D[15], m, L[6]);
+      L[7] = m2l_fma(D[17], m, L[7]);
+      L[8] = m2l_fma(D[18], m, L[8]);
+      L[9] = m2l_fma(D[21], m, L[9]);
+      L[10] = m2l_fma(D[23], m, L[10]);
+      L[11] = m2l_fma(D[24], m, L[11]);
+      L[12] = m2l_fma(D[26], m, L[12]);
+      L[13] = m2l_fma(D[27], m, L[13]);
+      L[14] = m2l_fma(D[29], m, L[14]);
+      L[15] = m2l_fma(D[30], m, L[15]);
+      L[16] = m2l_fma(D[33], m, L[16]);
+      L[17] = m2l_fma(D[35], m, L[17]);
+      L[18] = m2l_fma(D[36], m, L[18]);
+      L[19] = m2l_fma(D[38], m, L[19]);
+      L[20] = m2l_fma(D[39], m, L[20]);
+      L[21] = m2l_fma(D[41], m, L[21]);
+      L[22] = m2l_fma(D[42], m, L[22]);
+      L[23] = m2l_fma(D[44], m, L[23]);
+      L[24] = m2l_fma(D[45], m, L[24]);
     }
     rp *= rho;
-    { const float m = -__ldg(Mr + 9) * rp;
-      L[1] = fmaf(D[19], m, L[1]);
-      L[2] = fmaf(D[20], m, L[2]);
-      L[3] = fmaf(D[21], m, L[3]);
-      L[4] = fmaf(D[31], m, L[4]);
-      L[5] = fmaf(D[32], m, L[5]);
-      L[6] = fmaf(D[33], m, L[6]);
-      L[7] = fmaf(D[34], m, L[7]);
-      L[8] = fmaf(D[35], m, L[8]);
+    { const T m = __ldg(Mr + 4) * rp;
+      L[1] = m2l_fma(D[10], m, L[1]);
+      L[2] = m2l_fma(D[11], m, L[2]);
+      L[3] = m2l_fma(D[12], m, L[3]);
+      L[4] = m2l_fma(D[19], m, L[4]);
+      L[5] = m2l_fma(D[20], m, L[5]);
+      L[6] = m2l_fma(D[21], m, L[6]);
+      L[7] = m2l_fma(D[22], m, L[7]);
+      L[8] = m2l_fma(D[23], m, L[8]);
+      L[9] = m2l_fma(D[31], m, L[9]);
+      L[10] = m2l_fma(D[32], m, L[10]);
+      L[11] = m2l_fma(D[33], m, L[11]);
+      L[12] = m2l_fma(D[34], m, L[12]);
+      L[13] = m2l_fma(D[35], m, L[13]);
+      L[14] = m2l_fma(D[37], m, L[14]);
+      L[15] = m2l_fma(D[38], m, L[15]);
     }
-    { const float m = -__ldg(Mr + 10) * rp;
-      L[1] = fmaf(D[20], m, L[1]);
-      L[2] = fmaf(D[22], m, L[2]);
-      L[3] = fmaf(D[23], m, L[3]);
-      L[4] = fmaf(D[32], m, L[4]);
-      L[5] = fmaf(D[34], m, L[5]);
-      L[6] = fmaf(D[35], m, L[6]);
-      L[7] = fmaf(D[37], m, L[7]);
-      L[8] = fmaf(D[38], m, L[8]);
+    { const T m = __ldg(Mr + 5) * rp;
+      L[1] = m2l_fma(D[11], m, L[1]);
+      L[2] = m2l_fma(D[13], m, L[2]);
+      L[3] = m2l_fma(D[14], m, L[3]);
+      L[4] = m2l_fma(D[20], m, L[4]);
+      L[5] = m2l_fma(D[22], m, L[5]);
+      L[6] = m2l_fma(D[23], m, L[6]);
+      L[7] = m2l_fma(D[25], m, L[7]);
+      L[8] = m2l_fma(D[26], m, L[8]);
+      L[9] = m2l_fma(D[32], m, L[9]);
+      L[10] = m2l_fma(D[34], m, L[10]);
+      L[11] = m2l_fma(D[35], m, L[11]);
+      L[12] = m2l_fma(D[37], m, L[12]);
+      L[13] = m2l_fma(D[38], m, L[13]);
+      L[14] = m2l_fma(D[40], m, L[14]);
+      L[15] = m2l_fma(D[41], m, L[15]);
     }
-    { const float m = -__ldg(Mr + 11) * rp;
-      L[1] = fmaf(D[21], m, L[1]);
-      L[2] = fmaf(D[23], m, L[2]);
-      L[3] = fmaf(D[24], m, L[3]);
-      L[4] = fmaf(D[33], m, L[4]);
-      L[5] = fmaf(D[35], m, L[5]);
-      L[6] = fmaf(D[36], m, L[6]);
-      L[7] = fmaf(D[38], m, L[7]);
-      L[8] = fmaf(D[39], m, L[8]);
+    { const T m = __ldg(Mr + 6) * rp;
+      L[1] = m2l_fma(D[12], m, L[1]);
+      L[2] = m2l_fma(D[14], m, L[2]);
+      L[3] = m2l_fma(D[15], m, L[3]);
+      L[4] = m2l_fma(D[21], m, L[4]);
+      L[5] = m2l_fma(D[23], m, L[5]);
+      L[6] = m2l_fma(D[24], m, L[6]);
+      L[7] = m2l_fma(D[26], m, L[7]);
+      L[8] = m2l_fma(D[27], m, L[8]);
+      L[9] = m2l_fma(D[33], m, L[9]);
+      L[10] = m2l_fma(D[35], m, L[10]);
+      L[11] = m2l_fma(D[36], m, L[11]);
+      L[12] = m2l_fma(D[38], m, L[12]);
+      L[13] = m2l_fma(D[39], m, L[13]);
+      L[14] = m2l_fma(D[41], m, L[14]);
+      L[15] = m2l_fma(D[42], m, L[15]);
     }
-    { const float m = -__ldg(Mr + 12) * rp;
-      L[1] = fmaf(D[22], m, L[1]);
-      L[2] = fmaf(D[25], m, L[2]);
-      L[3] = fmaf(D[26], m, L[3]);
-      L[4] = fmaf(D[34], m, L[4]);
-      L[5] = fmaf(D[37], m, L[5]);
-      L[6] = fmaf(D[38], m, L[6]);
-      L[7] = fmaf(D[40], m, L[7]);
-      L[8] = fmaf(D[41], m, L[8]);
+    { const T m = __ldg(Mr + 7) * rp;
+      L[1] = m2l_fma(D[13], m, L[1]);
+      L[2] = m2l_fma(D[16], m, L[2]);
+      L[3] = m2l_fma(D[17], m, L[3]);
+      L[4] = m2l_fma(D[22], m, L[4]);
+      L[5] = m2l_fma(D[25], m, L[5]);
+      L[6] = m2l_fma(D[26], m, L[6]);
+      L[7] = m2l_fma(D[28], m, L[7]);
+      L[8] = m2l_fma(D[29], m, L[8]);
+      L[9] = m2l_fma(D[34], m, L[9]);
+      L[10] = m2l_fma(D[37], m, L[10]);
+      L[11] = m2l_fma(D[38], m, L[11]);
+      L[12] = m2l_fma(D[40], m, L[12]);
+      L[13] = m2l_fma(D[41], m, L[13]);
+      L[14] = m2l_fma(D[43], m, L[14]);
+      L[15] = m2l_fma(D[44], m, L[15]);
     }
-    { const float m = -__ldg(Mr + 13) * rp;
-      L[1] = fmaf(D[23], m, L[1]);
-      L[2] = fmaf(D[26], m, L[2]);
-      L[3] = fmaf(D[27], m, L[3]);
-      L[4] = fmaf(D[35], m, L[4]);
-      L[5] = fmaf(D[38], m, L[5]);
-      L[6] = fmaf(D[39], m, L[6]);
-      L[7] = fmaf(D[41], m, L[7]);
-      L[8] = fmaf(D[42], m, L[8]);
-    }
-    { const float m = -__ldg(Mr + 14) * rp;
-      L[1] = fmaf(D[25], m, L[1]);
-      L[2] = fmaf(D[28], m, L[2]);
-      L[3] = fmaf(D[29], m, L[3]);
-      L[4] = fmaf(D[37], m, L[4]);
-      L[5] = fmaf(D[40], m, L[5]);
-      L[6] = fmaf(D[41], m, L[6]);
-      L[7] = fmaf(D[43], m, L[7]);
-      L[8] = fmaf(D[44], m, L[8]);
-    }
-    { const float m = -__ldg(Mr + 15) * rp;
-      L[1] = fmaf(D[26], m, L[1]);
-      L[2] = fmaf(D[29], m, L[2]);
-      L[3] = fmaf(D[30], m, L[3]);
-      L[4] = fmaf(D[38], m, L[4]);
-      L[5] = fmaf(D[41], m, L[5]);
-      L[6] = fmaf(D[42], m, L[6]);
-      L[7] = fmaf(D[44], m, L[7]);
-      L[8] = fmaf(D[45], m, L[8]);
+    { const T m = __ldg(Mr + 8) * rp;
+      L[1] = m2l_fma(D[14], m, L[1]);
+      L[2] = m2l_fma(D[17], m, L[2]);
+      L[3] = m2l_fma(D[18], m, L[3]);
+      L[4] = m2l_fma(D[23], m, L[4]);
+      L[5] = m2l_fma(D[26], m, L[5]);
+      L[6] = m2l_fma(D[27], m, L[6]);
+      L[7] = m2l_fma(D[29], m, L[7]);
+      L[8] = m2l_fma(D[30], m, L[8]);
+      L[9] = m2l_fma(D[35], m, L[9]);
+      L[10] = m2l_fma(D[38], m, L[10]);
+      L[11] = m2l_fma(D[39], m, L[11]);
+      L[12] = m2l_fma(D[41], m, L[12]);
+      L[13] = m2l_fma(D[42], m, L[13]);
+      L[14] = m2l_fma(D[44], m, L[14]);
+      L[15] = m2l_fma(D[45], m, L[15]);
     }
     rp *= rho;
-    { const float m = __ldg(Mr + 16) * rp;
-      L[1] = fmaf(D[31], m, L[1]);
-      L[2] = fmaf(D[32], m, L[2]);
-      L[3] = fmaf(D[33], m, L[3]);
+    { const T m = -__ldg(Mr + 9) * rp;
+      L[1] = m2l_fma(D[19], m, L[1]);
+      L[2] = m2l_fma(D[20], m, L[2]);
+      L[3] = m2l_fma(D[21], m, L[3]);
+      L[4] = m2l_fma(D[31], m, L[4]);
+      L[5] = m2l_fma(D[32], m, L[5]);
+      L[6] = m2l_fma(D[33], m, L[6]);
+      L[7] = m2l_fma(D[34], m, L[7]);
+      L[8] = m2l_fma(D[35], m, L[8]);
     }
-    { const float m = __ldg(Mr + 17) * rp;
-      L[1] = fmaf(D[32], m, L[1]);
-      L[2] = fmaf(D[34], m, L[2]);
-      L[3] = fmaf(D[35], m, L[3]);
+    { const T m = -__ldg(Mr + 10) * rp;
+      L[1] = m2l_fma(D[20], m, L[1]);
+      L[2] = m2l_fma(D[22], m, L[2]);
+      L[3] = m2l_fma(D[23], m, L[3]);
+      L[4] = m2l_fma(D[32], m, L[4]);
+      L[5] = m2l_fma(D[34], m, L[5]);
+      L[6] = m2l_fma(D[35], m, L[6]);
+      L[7] = m2l_fma(D[37], m, L[7]);
+      L[8] = m2l_fma(D[38], m, L[8]);
     }
-    { const float m = __ldg(Mr + 18) * rp;
-      L[1] = fmaf(D[33], m, L[1]);
-      L[2] = fmaf(D[35], m, L[2]);
-      L[3] = fmaf(D[36], m, L[3]);
+    { const T m = -__ldg(Mr + 11) * rp;
+      L[1] = m2l_fma(D[21], m, L[1]);
+      L[2] = m2l_fma(D[23], m, L[2]);
+      L[3] = m2l_fma(D[24], m, L[3]);
+      L[4] = m2l_fma(D[33], m, L[4]);
+      L[5] = m2l_fma(D[35], m, L[5]);
+      L[6] = m2l_fma(D[36], m, L[6]);
+      L[7] = m2l_fma(D[38], m, L[7]);
+      L[8] = m2l_fma(D[39], m, L[8]);
     }
-    { const float m = __ldg(Mr + 19) * rp;
-      L[1] = fmaf(D[34], m, L[1]);
-      L[2] = fmaf(D[37], m, L[2]);
-      L[3] = fmaf(D[38], m, L[3]);
+    { const T m = -__ldg(Mr + 12) * rp;
+      L[1] = m2l_fma(D[22], m, L[1]);
+      L[2] = m2l_fma(D[25], m, L[2]);
+      L[3] = m2l_fma(D[26], m, L[3]);
+      L[4] = m2l_fma(D[34], m, L[4]);
+      L[5] = m2l_fma(D[37], m, L[5]);
+      L[6] = m2l_fma(D[38], m, L[6]);
+      L[7] = m2l_fma(D[40], m, L[7]);
+      L[8] = m2l_fma(D[41], m, L[8]);
     }
-    { const float m = __ldg(Mr + 20) * rp;
-      L[1] = fmaf(D[35], m, L[1]);
-      L[2] = fmaf(D[38], m, L[2]);
-      L[3] = fmaf(D[39], m, L[3]);
+    { const T m = -__ldg(Mr + 13) * rp;
+      L[1] = m2l_fma(D[23], m, L[1]);
+      L[2] = m2l_fma(D[26], m, L[2]);
+      L[3] = m2l_fma(D[27], m, L[3]);
+      L[4] = m2l_fma(D[35], m, L[4]);
+      L[5] = m2l_fma(D[38], m, L[5]);
+      L[6] = m2l_fma(D[39], m, L[6]);
+      L[7] = m2l_fma(D[41], m, L[7]);
+      L[8] = m2l_fma(D[42], m, L[8]);
     }
-    { const float m = __ldg(Mr + 21) * rp;
-      L[1] = fmaf(D[37], m, L[1]);
-      L[2] = fmaf(D[40], m, L[2]);
-      L[3] = fmaf(D[41], m, L[3]);
+    { const T m = -__ldg(Mr + 14) * rp;
+      L[1] = m2l_fma(D[25], m, L[1]);
+      L[2] = m2l_fma(D[28], m, L[2]);
+      L[3] = m2l_fma(D[29], m, L[3]);
+      L[4] = m2l_fma(D[37], m, L[4]);
+      L[5] = m2l_fma(D[40], m, L[5]);
+      L[6] = m2l_fma(D[41], m, L[6]);
+      L[7] = m2l_fma(D[43], m, L[7]);
+      L[8] = m2l_fma(D[44], m, L[8]);
     }
-    { const float m = __ldg(Mr + 22) * rp;
-      L[1] = fmaf(D[38], m, L[1]);
-      L[2] = fmaf(D[41], m, L[2]);
-      L[3] = fmaf(D[42], m, L[3]);
+    { const T m = -__ldg(Mr + 15) * rp;
+      L[1] = m2l_fma(D[26], m, L[1]);
+      L[2] = m2l_fma(D[29], m, L[2]);
+      L[3] = m2l_fma(D[30], m, L[3]);
+      L[4] = m2l_fma(D[38], m, L[4]);
+      L[5] = m2l_fma(D[41], m, L[5]);
+      L[6] = m2l_fma(D[42], m, L[6]);
+      L[7] = m2l_fma(D[44], m, L[7]);
+      L[8] = m2l_fma(D[45], m, L[8]);
     }
-    { const float m = __ldg(Mr + 23) * rp;
-      L[1] = fmaf(D[40], m, L[1]);
-      L[2] = fmaf(D[43], m, L[2]);
-      L[3] = fmaf(D[44], m, L[3]);
+    rp *= rho;
+    { const T m = __ldg(Mr + 16) * rp;
+      L[1] = m2l_fma(D[31], m, L[1]);
+      L[2] = m2l_fma(D[32], m, L[2]);
+      L[3] = m2l_fma(D[33], m, L[3]);
     }
-    { const float m = __ldg(Mr + 24) * rp;
-      L[1] = fmaf(D[41], m, L[1]);
-      L[2] = fmaf(D[44], m, L[2]);
-      L[3] = fmaf(D[45], m, L[3]);
+    { const T m = __ldg(Mr + 17) * rp;
+      L[1] = m2l_fma(D[32], m, L[1]);
+      L[2] = m2l_fma(D[34], m, L[2]);
+      L[3] = m2l_fma(D[35], m, L[3]);
+    }
+    { const T m = __ldg(Mr + 18) * rp;
+      L[1] = m2l_fma(D[33], m, L[1]);
+      L[2] = m2l_fma(D[35], m, L[2]);
+      L[3] = m2l_fma(D[36], m, L[3]);
+    }
+    { const T m = __ldg(Mr + 19) * rp;
+      L[1] = m2l_fma(D[34], m, L[1]);
+      L[2] = m2l_fma(D[37], m, L[2]);
+      L[3] = m2l_fma(D[38], m, L[3]);
+    }
+    { const T m = __ldg(Mr + 20) * rp;
+      L[1] = m2l_fma(D[35], m, L[1]);
+      L[2] = m2l_fma(D[38], m, L[2]);
+      L[3] = m2l_fma(D[39], m, L[3]);
+    }
+    { const T m = __ldg(Mr + 21) * rp;
+      L[1] = m2l_fma(D[37], m, L[1]);
+      L[2] = m2l_fma(D[40], m, L[2]);
+      L[3] = m2l_fma(D[41], m, L[3]);
+    }
+    { const T m = __ldg(Mr + 22) * rp;
+      L[1] = m2l_fma(D[38], m, L[1]);
+      L[2] = m2l_fma(D[41], m, L[2]);
+      L[3] = m2l_fma(D[42], m, L[3]);
+    }
+    { const T m = __ldg(Mr + 23) * rp;
+      L[1] = m2l_fma(D[40], m, L[1]);
+      L[2] = m2l_fma(D[43], m, L[2]);
+      L[3] = m2l_fma(D[44], m, L[3]);
+    }
+    { const T m = __ldg(Mr + 24) * rp;
+      L[1] = m2l_fma(D[41], m, L[1]);
+      L[2] = m2l_fma(D[44], m, L[2]);
+      L[3] = m2l_fma(D[45], m, L[3]);
     }
 }
 
-__device__ __forceinline__ void m2l_side_b_h_forces_5(const float (&D)[46], const float *__restrict__ Mr, float (&L)[36])
+template <class T> __device__ __forceinline__ void m2l_side_b_h_forces_5(const T (&D)[46], const T *__restrict__ Mr, T (&L)[36])
 {
-    L[0] = 0.0f;
-    { const float m = __ldg(Mr + 0);
+    L[0] = T(0);
+    { const T m = __ldg(Mr + 0);
       L[1] = -D[1] * m;
       L[2] = -D[2] * m;
       L[3] = -D[3] * m;
@@ -13225,344 +13225,344 @@ __device__ __forceinline__ void m2l_side_b_h_forces_5(const float (&D)[46], cons
       L[34] = -D[43] * m;
       L[35] = -D[44] * m;
     }
-    { const float m = __ldg(Mr + 1);
-      L[1] = fmaf(-D[4], m, L[1]);
-      L[2] = fmaf(-D[5], m, L[2]);
-      L[3] = fmaf(-D[6], m, L[3]);
-      L[4] = fmaf(D[10], m, L[4]);
-      L[5] = fmaf(D[11], m, L[5]);
-      L[6] = fmaf(D[12], m, L[6]);
-      L[7] = fmaf(D[13], m, L[7]);
-      L[8] = fmaf(D[14], m, L[8]);
-      L[9] = fmaf(-D[19], m, L[9]);
-      L[10] = fmaf(-D[20], m, L[10]);
-      L[11] = fmaf(-D[21], m, L[11]);
-      L[12] = fmaf(-D[22], m, L[12]);
-      L[13] = fmaf(-D[23], m, L[13]);
-      L[14] = fmaf(-D[25], m, L[14]);
-      L[15] = fmaf(-D[26], m, L[15]);
-      L[16] = fmaf(D[31], m, L[16]);
-      L[17] = fmaf(D[32], m, L[17]);
-      L[18] = fmaf(D[33], m, L[18]);
-      L[19] = fmaf(D[34], m, L[19]);
-      L[20] = fmaf(D[35], m, L[20]);
-      L[21] = fmaf(D[37], m, L[21]);
-      L[22] = fmaf(D[38], m, L[22]);
-      L[23] = fmaf(D[40], m, L[23]);
-      L[24] = fmaf(D[41], m, L[24]);
+    { const T m = __ldg(Mr + 1);
+      L[1] = m2l_fma(-D[4], m, L[1]);
+      L[2] = m2l_fma(-D[5], m, L[2]);
+      L[3] = m2l_fma(-D[6], m, L[3]);
+      L[4] = m2l_fma(D[10], m, L[4]);
+      L[5] = m2l_fma(D[11], m, L[5]);
+      L[6] = m2l_fma(D[12], m, L[6]);
+      L[7] = m2l_fma(D[13], m, L[7]);
+      L[8] = m2l_fma(D[14], m, L[8]);
+      L[9] = m2l_fma(-D[19], m, L[9]);
+      L[10] = m2l_fma(-D[20], m, L[10]);
+      L[11] = m2l_fma(-D[21], m, L[11]);
+      L[12] = m2l_fma(-D[22], m, L[12]);
+      L[13] = m2l_fma(-D[23], m, L[13]);
+      L[14] = m2l_fma(-D[25], m, L[14]);
+      L[15] = m2l_fma(-D[26], m, L[15]);
+      L[16] = m2l_fma(D[31], m, L[16]);
+      L[17] = m2l_fma(D[32], m, L[17]);
+      L[18] = m2l_fma(D[33], m, L[18]);
+      L[19] = m2l_fma(D[34], m, L[19]);
+      L[20] = m2l_fma(D[35], m, L[20]);
+      L[21] = m2l_fma(D[37], m, L[21]);
+      L[22] = m2l_fma(D[38], m, L[22]);
+      L[23] = m2l_fma(D[40], m, L[23]);
+      L[24] = m2l_fma(D[41], m, L[24]);
     }
-    { const float m = __ldg(Mr + 2);
-      L[1] = fmaf(-D[5], m, L[1]);
-      L[2] = fmaf(-D[7], m, L[2]);
-      L[3] = fmaf(-D[8], m, L[3]);
-      L[4] = fmaf(D[11], m, L[4]);
-      L[5] = fmaf(D[13], m, L[5]);
-      L[6] = fmaf(D[14], m, L[6]);
-      L[7] = fmaf(D[16], m, L[7]);
-      L[8] = fmaf(D[17], m, L[8]);
-      L[9] = fmaf(-D[20], m, L[9]);
-      L[10] = fmaf(-D[22], m, L[10]);
-      L[11] = fmaf(-D[23], m, L[11]);
-      L[12] = fmaf(-D[25], m, L[12]);
-      L[13] = fmaf(-D[26], m, L[13]);
-      L[14] = fmaf(-D[28], m, L[14]);
-      L[15] = fmaf(-D[29], m, L[15]);
-      L[16] = fmaf(D[32], m, L[16]);
-      L[17] = fmaf(D[34], m, L[17]);
-      L[18] = fmaf(D[35], m, L[18]);
-      L[19] = fmaf(D[37], m, L[19]);
-      L[20] = fmaf(D[38], m, L[20]);
-      L[21] = fmaf(D[40], m, L[21]);
-      L[22] = fmaf(D[41], m, L[22]);
-      L[23] = fmaf(D[43], m, L[23]);
-      L[24] = fmaf(D[44], m, L[24]);
+    { const T m = __ldg(Mr + 2);
+      L[1] = m2l_fma(-D[5], m, L[1]);
+      L[2] = m2l_fma(-D[7], m, L[2]);
+      L[3] = m2l_fma(-D[8], m, L[3]);
+      L[4] = m2l_fma(D[11], m, L[4]);
+      L[5] = m2l_fma(D[13], m, L[5]);
+      L[6] = m2l_fma(D[14], m, L[6]);
+      L[7] = m2l_fma(D[16], m, L[7]);
+      L[8] = m2l_fma(D[17], m, L[8]);
+      L[9] = m2l_fma(-D[20], m, L[9]);
+      L[10] = m2l_fma(-D[22], m, L[10]);
+      L[11] = m2l_fma(-D[23], m, L[11]);
+      L[12] = m2l_fma(-D[25], m, L[12]);
+      L[13] = m2l_fma(-D[26], m, L[13]);
+      L[14] = m2l_fma(-D[28], m, L[14]);
+      L[15] = m2l_fma(-D[29], m, L[15]);
+      L[16] = m2l_fma(D[32], m, L[16]);
+      L[17] = m2l_fma(D[34], m, L[17]);
+      L[18] = m2l_fma(D[35], m, L[18]);
+      L[19] = m2l_fma(D[37], m, L[19]);
+      L[20] = m2l_fma(D[38], m, L[20]);
+      L[21] = m2l_fma(D[40], m, L[21]);
+      L[22] = m2l_fma(D[41], m, L[22]);
+      L[23] = m2l_fma(D[43], m, L[23]);
+      L[24] = m2l_fma(D[44], m, L[24]);
     }
-    { const float m = __ldg(Mr + 3);
-      L[1] = fmaf(-D[6], m, L[1]);
-      L[2] = fmaf(-D[8], m, L[2]);
-      L[3] = fmaf(-D[9], m, L[3]);
-      L[4] = fmaf(D[12], m, L[4]);
-      L[5] = fmaf(D[14], m, L[5]);
-      L[6] = fmaf(D[15], m, L[6]);
-      L[7] = fmaf(D[17], m, L[7]);
-      L[8] = fmaf(D[18], m, L[8]);
-      L[9] = fmaf(-D[21], m, L[9]);
-      L[10] = fmaf(-D[23], m, L[10]);
-      L[11] = fmaf(-D[24], m, L[11]);
-      L[12] = fmaf(-D[26], m, L[12]);
-      L[13] = fmaf(-D[27], m, L[13]);
-      L[14] = fmaf(-D[29], m, L[14]);
-      L[15] = fmaf(-D[30], m, L[15]);
-      L[16] = fmaf(D[33], m, L[16]);
-      L[17] = fmaf(D[35], m, L[17]);
-      L[18] = fmaf(D[36], m, L[18]);
-      L[19] = fmaf(D[38], m, L[19]);
-      L[20] = fmaf(D[39], m, L[20]);
-      L[21] = fmaf(D[41], m, L[21]);
-      L[22] = fmaf(D[42], m, L[22]);
-      L[23] = fmaf(D[44], m, L[23]);
-      L[24] = fmaf(D[45], m, L[24]);
+    { const T m = __ldg(Mr + 3);
+      L[1] = m2l_fma(-D[6], m, L[1]);
+      L[2] = m2l_fma(-D[8], m, L[2]);
+      L[3] = m2l_fma(-D[9], m, L[3]);
+      L[4] = m2l_fma(D[12], m, L[4]);
+      L[5] = m2l_fma(D[14], m, L[5]);
+      L[6] = m2l_fma(D[15], m, L[6]);
+      L[7] = m2l_fma(D[17], m, L[7]);
+      L[8] = m2l_fma(D[18], m, L[8]);
+      L[9] = m2l_fma(-D[21], m, L[9]);
+      L[10] = m2l_fma(-D[23], m, L[10]);
+      L[11] = m2l_fma(-D[24], m, L[11]);
+      L[12] = m2l_fma(-D[26], m, L[12]);
+      L[13] = m2l_fma(-D[27], m, L[13]);
+      L[14] = m2l_fma(-D[29], m, L[14]);
+      L[15] = m2l_fma(-D[30], m, L[15]);
+      L[16] = m2l_fma(D[33], m, L[16]);
+      L[17] = m2l_fma(D[35], m, L[17]);
+      L[18] = m2l_fma(D[36], m, L[18]);
+      L[19] = m2l_fma(D[38], m, L[19]);
+      L[20] = m2l_fma(D[39], m, L[20]);
+      L[21] = m2l_fma(D[41], m, L[21]);
+      L[22] = m2l_fma(D[42], m, L[22]);
+      L[23] = m2l_fma(D[44], m, L[23]);
+      L[24] = m2l_fma(D[45], m, L[24]);
     }
-    { const float m = __ldg(Mr + 4);
-      L[1] = fmaf(-D[10], m, L[1]);
-      L[2] = fmaf(-D[11], m, L[2]);
-      L[3] = fmaf(-D[12], m, L[3]);
-      L[4] = fmaf(D[19], m, L[4]);
-      L[5] = fmaf(D[20], m, L[5]);
-      L[6] = fmaf(D[21], m, L[6]);
-      L[7] = fmaf(D[22], m, L[7]);
-      L[8] = fmaf(D[23], m, L[8]);
-      L[9] = fmaf(-D[31], m, L[9]);
-      L[10] = fmaf(-D[32], m, L[10]);
-      L[11] = fmaf(-D[33], m, L[11]);
-      L[12] = fmaf(-D[34], m, L[12]);
-      L[13] = fmaf(-D[35], m, L[13]);
-      L[14] = fmaf(-D[37], m, L[14]);
-      L[15] = fmaf(-D[38], m, L[15]);
+    { const T m = __ldg(Mr + 4);
+      L[1] = m2l_fma(-D[10], m, L[1]);
+      L[2] = m2l_fma(-D[11], m, L[2]);
+      L[3] = m2l_fma(-D[12], m, L[3]);
+      L[4] = m2l_fma(D[19], m, L[4]);
+      L[5] = m2l_fma(D[20], m, L[5]);
+      L[6] = m2l_fma(D[21], m, L[6]);
+      L[7] = m2l_fma(D[22], m, L[7]);
+      L[8] = m2l_fma(D[23], m, L[8]);
+      L[9] = m2l_fma(-D[31], m, L[9]);
+      L[10] = m2l_fma(-D[32], m, L[10]);
+      L[11] = m2l_fma(-D[33], m, L[11]);
+      L[12] = m2l_fma(-D[34], m, L[12]);
+      L[13] = m2l_fma(-D[35], m, L[13]);
+      L[14] = m2l_fma(-D[37], m, L[14]);
+      L[15] = m2l_fma(-D[38], m, L[15]);
     }
-    { const float m = __ldg(Mr + 5);
-      L[1] = fmaf(-D[11], m, L[1]);
-      L[2] = fmaf(-D[13], m, L[2]);
-      L[3] = fmaf(-D[14], m, L[3]);
-      L[4] = fmaf(D[20], m, L[4]);
-      L[5] = fmaf(D[22], m, L[5]);
-      L[6] = fmaf(D[23], m, L[6]);
-      L[7] = fmaf(D[25], m, L[7]);
-      L[8] = fmaf(D[26], m, L[8]);
-      L[9] = fmaf(-D[32], m, L[9]);
-      L[10] = fmaf(-D[34], m, L[10]);
-      L[11] = fmaf(-D[35], m, L[11]);
-      L[12] = fmaf(-D[37], m, L[12]);
-      L[13] = fmaf(-D[38], m, L[13]);
-      L[14] = fmaf(-D[40], m, L[14]);
-      L[15] = fmaf(-D[41], m, L[15]);
+    { const T m = __ldg(Mr + 5);
+      L[1] = m2l_fma(-D[11], m, L[1]);
+      L[2] = m2l_fma(-D[13], m, L[2]);
+      L[3] = m2l_fma(-D[14], m, L[3]);
+      L[4] = m2l_fma(D[20], m, L[4]);
+      L[5] = m2l_fma(D[22], m, L[5]);
+      L[6] = m2l_fma(D[23], m, L[6]);
+      L[7] = m2l_fma(D[25], m, L[7]);
+      L[8] = m2l_fma(D[26], m, L[8]);
+      L[9] = m2l_fma(-D[32], m, L[9]);
+      L[10] = m2l_fma(-D[34], m, L[10]);
+      L[11] = m2l_fma(-D[35], m, L[11]);
+      L[12] = m2l_fma(-D[37], m, L[12]);
+      L[13] = m2l_fma(-D[38], m, L[13]);
+      L[14] = m2l_fma(-D[40], m, L[14]);
+      L[15] = m2l_fma(-D[41], m, L[15]);
     }
-    { const float m = __ldg(Mr + 6);
-      L[1] = fmaf(-D[12], m, L[1]);
-      L[2] = fmaf(-D[14], m, L[2]);
-      L[3] = fmaf(-D[15], m, L[3]);
-      L[4] = fmaf(D[21], m, L[4]);
-      L[5] = fmaf(D[23], m, L[5]);
-      L[6] = fmaf(D[24], m, L[6]);
-      L[7] = fmaf(D[26], m, L[7]);
-      L[8] = fmaf(D[27], m, L[8]);
-      L[9] = fmaf(-D[33], m, L[9]);
-      L[10] = fmaf(-D[35], m, L[10]);
-      L[11] = fmaf(-D[36], m, L[11]);
-      L[12] = fmaf(-D[38], m, L[12]);
-      L[13] = fmaf(-D[39], m, L[13]);
-      L[14] = fmaf(-D[41], m, L[14]);
-      L[15] = fmaf(-D[42], m, L[15]);
+    { const T m = __ldg(Mr + 6);
+      L[1] = m2l_fma(-D[12], m, L[1]);
+      L[2] = m2l_fma(-D[14], m, L[2]);
+      L[3] = m2l_fma(-D[15], m, L[3]);
+      L[4] = m2l_fma(D[21], m, L[4]);
+      L[5] = m2l_fma(D[23], m, L[5]);
+      L[6] = m2l_fma(D[24], m, L[6]);
+      L[7] = m2l_fma(D[26], m, L[7]);
+      L[8] = m2l_fma(D[27], m, L[8]);
+      L[9] = m2l_fma(-D[33], m, L[9]);
+      L[10] = m2l_fma(-D[35], m, L[10]);
+      L[11] = m2l_fma(-D[36], m, L[11]);
+      L[12] = m2l_fma(-D[38], m, L[12]);
+      L[13] = m2l_fma(-D[39], m, L[13]);
+      L[14] = m2l_fma(-D[41], m, L[14]);
+      L[15] = m2l_fma(-D[42], m, L[15]);
     }
-    { const float m = __ldg(Mr + 7);
-      L[1] = fmaf(-D[13], m, L[1]);
-      L[2] = fmaf(-D[16], m, L[2]);
-      L[3] = fmaf(-D[17], m, L[3]);
-      L[4] = fmaf(D[22], m, L[4]);
-      L[5] = fmaf(D[25], m, L[5]);
-      L[6] = fmaf(D[26], m, L[6]);
-      L[7] = fmaf(D[28], m, L[7]);
-      L[8] = fmaf(D[29], m, L[8]);
-      L[9] = fmaf(-D[34], m, L[9]);
-      L[10] = fmaf(-D[37], m, L[10]);
-      L[11] = fmaf(-D[38], m, L[11]);
-      L[12] = fmaf(-D[40], m, L[12]);
-      L[13] = fmaf(-D[41], m, L[13]);
-      L[14] = fmaf(-D[43], m, L[14]);
-      L[15] = fmaf(-D[44], m, L[15]);
+    { const T m = __ldg(Mr + 7);
+      L[1] = m2l_fma(-D[13], m, L[1]);
+      L[2] = m2l_fma(-D[16], m, L[2]);
+      L[3] = m2l_fma(-D[17], m, L[3]);
+      L[4] = m2l_fma(D[22], m, L[4]);
+      L[5] = m2l_fma(D[25], m, L[5]);
+      L[6] = m2l_fma(D[26], m, L[6]);
+      L[7] = m2l_fma(D[28], m, L[7]);
+      L[8] = m2l_fma(D[29], m, L[8]);
+      L[9] = m2l_fma(-D[34], m, L[9]);
+      L[10] = m2l_fma(-D[37], m, L[10]);
+      L[11] = m2l_fma(-D[38], m, L[11]);
+      L[12] = m2l_fma(-D[40], m, L[12]);
+      L[13] = m2l_fma(-D[41], m, L[13]);
+      L[14] = m2l_fma(-D[43], m, L[14]);
+      L[15] = m2l_fma(-D[44], m, L[15]);
     }
-    { const float m = __ldg(Mr + 8);
-      L[1] = fmaf(-D[14], m, L[1]);
-      L[2] = fmaf(-D[17], m, L[2]);
-      L[3] = fmaf(-D[18], m, L[3]);
-      L[4] = fmaf(D[23], m, L[4]);
-      L[5] = fmaf(D[26], m, L[5]);
-      L[6] = fmaf(D[27], m, L[6]);
-      L[7] = fmaf(D[29], m, L[7]);
-      L[8] = fmaf(D[30], m, L[8]);
-      L[9] = fmaf(-D[35], m, L[9]);
-      L[10] = fmaf(-D[38], m, L[10]);
-      L[11] = fmaf(-D[39], m, L[11]);
-      L[12] = fmaf(-D[41], m, L[12]);
-      L[13] = fmaf(-D[42], m, L[13]);
-      L[14] = fmaf(-D[44], m, L[14]);
-      L[15] = fmaf(-D[45], m, L[15]);
+    { const T m = __ldg(Mr + 8);
+      L[1] = m2l_fma(-D[14], m, L[1]);
+      L[2] = m2l_fma(-D[17], m, L[2]);
+      L[3] = m2l_fma(-D[18], m, L[3]);
+      L[4] = m2l_fma(D[23], m, L[4]);
+      L[5] = m2l_fma(D[26], m, L[5]);
+      L[6] = m2l_fma(D[27], m, L[6]);
+      L[7] = m2l_fma(D[29], m, L[7]);
+      L[8] = m2l_fma(D[30], m, L[8]);
+      L[9] = m2l_fma(-D[35], m, L[9]);
+      L[10] = m2l_fma(-D[38], m, L[10]);
+      L[11] = m2l_fma(-D[39], m, L[11]);
+      L[12] = m2l_fma(-D[41], m, L[12]);
+      L[13] = m2l_fma(-D[42], m, L[13]);
+      L[14] = m2l_fma(-D[44], m, L[14]);
+      L[15] = m2l_fma(-D[45], m, L[15]);
     }
-    { const float m = __ldg(Mr + 9);
-      L[1] = fmaf(-D[19], m, L[1]);
-      L[2] = fmaf(-D[20], m, L[2]);
-      L[3] = fmaf(-D[21], m, L[3]);
-      L[4] = fmaf(D[31], m, L[4]);
-      L[5] = fmaf(D[32], m, L[5]);
-      L[6] = fmaf(D[33], m, L[6]);
-      L[7] = fmaf(D[34], m, L[7]);
-      L[8] = fmaf(D[35], m, L[8]);
+    { const T m = __ldg(Mr + 9);
+      L[1] = m2l_fma(-D[19], m, L[1]);
+      L[2] = m2l_fma(-D[20], m, L[2]);
+      L[3] = m2l_fma(-D[21], m, L[3]);
+      L[4] = m2l_fma(D[31], m, L[4]);
+      L[5] = m2l_fma(D[32], m, L[5]);
+      L[6] = m2l_fma(D[33], m, L[6]);
+      L[7] = m2l_fma(D[34], m, L[7]);
+      L[8] = m2l_fma(D[35], m, L[8]);
     }
-    { const float m = __ldg(Mr + 10);
-      L[1] = fmaf(-D[20], m, L[1]);
-      L[2] = fmaf(-D[22], m, L[2]);
-      L[3] = fmaf(-D[23], m, L[3]);
-      L[4] = fmaf(D[32], m, L[4]);
-      L[5] = fmaf(D[34], m, L[5]);
-      L[6] = fmaf(D[35], m, L[6]);
-      L[7] = fmaf(D[37], m, L[7]);
-      L[8] = fmaf(D[38], m, L[8]);
+    { const T m = __ldg(Mr + 10);
+      L[1] = m2l_fma(-D[20], m, L[1]);
+      L[2] = m2l_fma(-D[22], m, L[2]);
+      L[3] = m2l_fma(-D[23], m, L[3]);
+      L[4] = m2l_fma(D[32], m, L[4]);
+      L[5] = m2l_fma(D[34], m, L[5]);
+      L[6] = m2l_fma(D[35], m, L[6]);
+      L[7] = m2l_fma(D[37], m, L[7]);
+      L[8] = m2l_fma(D[38], m, L[8]);
     }
-    { const float m = __ldg(Mr + 11);
-      L[1] = fmaf(-D[21], m, L[1]);
-      L[2] = fmaf(-D[23], m, L[2]);
-      L[3] = fmaf(-D[24], m, L[3]);
-      L[4] = fmaf(D[33], m, L[4]);
-      L[5] = fmaf(D[35], m, L[5]);
-      L[6] = fmaf(D[36], m, L[6]);
-      L[7] = fmaf(D[38], m, L[7]);
-      L[8] = fmaf(D[39], m, L[8]);
+    { const T m = __ldg(Mr + 11);
+      L[1] = m2l_fma(-D[21], m, L[1]);
+      L[2] = m2l_fma(-D[23], m, L[2]);
+      L[3] = m2l_fma(-D[24], m, L[3]);
+      L[4] = m2l_fma(D[33], m, L[4]);
+      L[5] = m2l_fma(D[35], m, L[5]);
+      L[6] = m2l_fma(D[36], m, L[6]);
+      L[7] = m2l_fma(D[38], m, L[7]);
+      L[8] = m2l_fma(D[39], m, L[8]);
     }
-    { const float m = __ldg(Mr + 12);
-      L[1] = fmaf(-D[22], m, L[1]);
-      L[2] = fmaf(-D[25], m, L[2]);
-      L[3] = fmaf(-D[26], m, L[3]);
-      L[4] = fmaf(D[34], m, L[4]);
-      L[5] = fmaf(D[37], m, L[5]);
-      L[6] = fmaf(D[38], m, L[6]);
-      L[7] = fmaf(D[40], m, L[7]);
-      L[8] = fmaf(D[41], m, L[8]);
+    { const T m = __ldg(Mr + 12);
+      L[1] = m2l_fma(-D[22], m, L[1]);
+      L[2] = m2l_fma(-D[25], m, L[2]);
+      L[3] = m2l_fma(-D[26], m, L[3]);
+      L[4] = m2l_fma(D[34], m, L[4]);
+      L[5] = m2l_fma(D[37], m, L[5]);
+      L[6] = m2l_fma(D[38], m, L[6]);
+      L[7] = m2l_fma(D[40], m, L[7]);
+      L[8] = m2l_fma(D[41], m, L[8]);
     }
-    { const float m = __ldg(Mr + 13);
-      L[1] = fmaf(-D[23], m, L[1]);
-      L[2] = fmaf(-D[26], m, L[2]);
-      L[3] = fmaf(-D[27], m, L[3]);
-      L[4] = fmaf(D[35], m, L[4]);
-      L[5] = fmaf(D[38], m, L[5]);
-      L[6] = fmaf(D[39], m, L[6]);
-      L[7] = fmaf(D[41], m, L[7]);
-      L[8] = fmaf(D[42], m, L[8]);
+    { const T m = __ldg(Mr + 13);
+      L[1] = m2l_fma(-D[23], m, L[1]);
+      L[2] = m2l_fma(-D[26], m, L[2]);
+      L[3] = m2l_fma(-D[27], m, L[3]);
+      L[4] = m2l_fma(D[35], m, L[4]);
+      L[5] = m2l_fma(D[38], m, L[5]);
+      L[6] = m2l_fma(D[39], m, L[6]);
+      L[7] = m2l_fma(D[41], m, L[7]);
+      L[8] = m2l_fma(D[42], m, L[8]);
     }
-    { const float m = __ldg(Mr + 14);
-      L[1] = fmaf(-D[25], m, L[1]);
-      L[2] = fmaf(-D[28], m, L[2]);
-      L[3] = fmaf(-D[29], m, L[3]);
-      L[4] = fmaf(D[37], m, L[4]);
-      L[5] = fmaf(D[40], m, L[5]);
-      L[6] = fmaf(D[41], m, L[6]);
-      L[7] = fmaf(D[43], m, L[7]);
-      L[8] = fmaf(D[44], m, L[8]);
+    { const T m = __ldg(Mr + 14);
+      L[1] = m2l_fma(-D[25], m, L[1]);
+      L[2] = m2l_fma(-D[28], m, L[2]);
+      L[3] = m2l_fma(-D[29], m, L[3]);
+      L[4] = m2l_fma(D[37], m, L[4]);
+      L[5] = m2l_fma(D[40], m, L[5]);
+      L[6] = m2l_fma(D[41], m, L[6]);
+      L[7] = m2l_fma(D[43], m, L[7]);
+      L[8] = m2l_fma(D[44], m, L[8]);
     }
-    { const float m = __ldg(Mr + 15);
-      L[1] = fmaf(-D[26], m, L[1]);
-      L[2] = fmaf(-D[29], m, L[2]);
-      L[3] = fmaf(-D[30], m, L[3]);
-      L[4] = fmaf(D[38], m, L[4]);
-      L[5] = fmaf(D[41], m, L[5]);
-      L[6] = fmaf(D[42], m, L[6]);
-      L[7] = fmaf(D[44], m, L[7]);
-      L[8] = fmaf(D[45], m, L[8]);
+    { const T m = __ldg(Mr + 15);
+      L[1] = m2l_fma(-D[26], m, L[1]);
+      L[2] = m2l_fma(-D[29], m, L[2]);
+      L[3] = m2l_fma(-D[30], m, L[3]);
+      L[4] = m2l_fma(D[38], m, L[4]);
+      L[5] = m2l_fma(D[41], m, L[5]);
+      L[6] = m2l_fma(D[42], m, L[6]);
+      L[7] = m2l_fma(D[44], m, L[7]);
+      L[8] = m2l_fma(D[45], m, L[8]);
     }
-    { const float m = __ldg(Mr + 16);
-      L[1] = fmaf(-D[31], m, L[1]);
-      L[2] = fmaf(-D[32], m, L[2]);
-      L[3] = fmaf(-D[33], m, L[3]);
+    { const T m = __ldg(Mr + 16);
+      L[1] = m2l_fma(-D[31], m, L[1]);
+      L[2] = m2l_fma(-D[32], m, L[2]);
+      L[3] = m2l_fma(-D[33], m, L[3]);
     }
-    { const float m = __ldg(Mr + 17);
-      L[1] = fmaf(-D[32], m, L[1]);
-      L[2] = fmaf(-D[34], m, L[2]);
-      L[3] = fmaf(-D[35], m, L[3]);
+    { const T m = __ldg(Mr + 17);
+      L[1] = m2l_fma(-D[32], m, L[1]);
+      L[2] = m2l_fma(-D[34], m, L[2]);
+      L[3] = m2l_fma(-D[35], m, L[3]);
     }
-    { const float m = __ldg(Mr + 18);
-      L[1] = fmaf(-D[33], m, L[1]);
-      L[2] = fmaf(-D[35], m, L[2]);
-      L[3] = fmaf(-D[36], m, L[3]);
+    { const T m = __ldg(Mr + 18);
+      L[1] = m2l_fma(-D[33], m, L[1]);
+      L[2] = m2l_fma(-D[35], m, L[2]);
+      L[3] = m2l_fma(-D[36], m, L[3]);
     }
-    { const float m = __ldg(Mr + 19);
-      L[1] = fmaf(-D[34], m, L[1]);
-      L[2] = fmaf(-D[37], m, L[2]);
-      L[3] = fmaf(-D[38], m, L[3]);
+    { const T m = __ldg(Mr + 19);
+      L[1] = m2l_fma(-D[34], m, L[1]);
+      L[2] = m2l_fma(-D[37], m, L[2]);
+      L[3] = m2l_fma(-D[38], m, L[3]);
     }
-    { const float m = __ldg(Mr + 20);
-      L[1] = fmaf(-D[35], m, L[1]);
-      L[2] = fmaf(-D[38], m, L[2]);
-      L[3] = fmaf(-D[39], m, L[3]);
+    { const T m = __ldg(Mr + 20);
+      L[1] = m2l_fma(-D[35], m, L[1]);
+      L[2] = m2l_fma(-D[38], m, L[2]);
+      L[3] = m2l_fma(-D[39], m, L[3]);
     }
-    { const float m = __ldg(Mr + 21);
-      L[1] = fmaf(-D[37], m, L[1]);
-      L[2] = fmaf(-D[40], m, L[2]);
-      L[3] = fmaf(-D[41], m, L[3]);
+    { const T m = __ldg(Mr + 21);
+      L[1] = m2l_fma(-D[37], m, L[1]);
+      L[2] = m2l_fma(-D[40], m, L[2]);
+      L[3] = m2l_fma(-D[41], m, L[3]);
     }
-    { const float m = __ldg(Mr + 22);
-      L[1] = fmaf(-D[38], m, L[1]);
-      L[2] = fmaf(-D[41], m, L[2]);
-      L[3] = fmaf(-D[42], m, L[3]);
+    { const T m = __ldg(Mr + 22);
+      L[1] = m2l_fma(-D[38], m, L[1]);
+      L[2] = m2l_fma(-D[41], m, L[2]);
+      L[3] = m2l_fma(-D[42], m, L[3]);
     }
-    { const float m = __ldg(Mr + 23);
-      L[1] = fmaf(-D[40], m, L[1]);
-      L[2] = fmaf(-D[43], m, L[2]);
-      L[3] = fmaf(-D[44], m, L[3]);
+    { const T m = __ldg(Mr + 23);
+      L[1] = m2l_fma(-D[40], m, L[1]);
+      L[2] = m2l_fma(-D[43], m, L[2]);
+      L[3] = m2l_fma(-D[44], m, L[3]);
     }
-    { const float m = __ldg(Mr + 24);
-      L[1] = fmaf(-D[41], m, L[1]);
-      L[2] = fmaf(-D[44], m, L[2]);
-      L[3] = fmaf(-D[45], m, L[3]);
+    { const T m = __ldg(Mr + 24);
+      L[1] = m2l_fma(-D[41], m, L[1]);
+      L[2] = m2l_fma(-D[44], m, L[2]);
+      L[3] = m2l_fma(-D[45], m, L[3]);
     }
 }
 
-__device__ __forceinline__ void m2l_reduce_moments_h_5(const float *__restrict__ Ms, float *__restrict__ Mr)
+template <class T> __device__ __forceinline__ void m2l_reduce_moments_h_5(const T *__restrict__ Ms, T *__restrict__ Mr)
 {
-    float v0 = Ms[0];
-    float v1 = Ms[1];
-    float v2 = Ms[2];
-    float v3 = Ms[3];
-    float v4 = Ms[4];
-    float v5 = Ms[5];
-    float v6 = Ms[6];
-    float v7 = Ms[7];
-    float v8 = Ms[8];
-    float v9 = Ms[9];
-    float v10 = Ms[10];
-    float v11 = Ms[11];
-    float v12 = Ms[12];
-    float v13 = Ms[13];
-    float v14 = Ms[14];
-    float v15 = Ms[15];
-    float v16 = Ms[16];
-    float v17 = Ms[17];
-    float v18 = Ms[18];
-    float v19 = Ms[19];
-    float v20 = Ms[20];
-    float v21 = Ms[21];
-    float v22 = Ms[22];
-    float v23 = Ms[23];
-    float v24 = Ms[24];
-    float v25 = Ms[25];
-    float v26 = Ms[26];
-    float v27 = Ms[27];
-    float v28 = Ms[28];
-    float v29 = Ms[29];
-    float v30 = Ms[30];
-    float v31 = Ms[31];
-    float v32 = Ms[32];
-    float v33 = Ms[33];
-    float v34 = Ms[34];
-    float v35 = Ms[35];
-    float v36 = Ms[36];
-    float v37 = Ms[37];
-    float v38 = Ms[38];
-    float v39 = Ms[39];
-    float v40 = Ms[40];
-    float v41 = Ms[41];
-    float v42 = Ms[42];
-    float v43 = Ms[43];
-    float v44 = Ms[44];
-    float v45 = Ms[45];
-    float v46 = Ms[46];
-    float v47 = Ms[47];
-    float v48 = Ms[48];
-    float v49 = Ms[49];
-    float v50 = Ms[50];
-    float v51 = Ms[51];
-    float v52 = Ms[52];
-    float v53 = Ms[53];
-    float v54 = Ms[54];
-    float v55 = Ms[55];
+    T v0 = Ms[0];
+    T v1 = Ms[1];
+    T v2 = Ms[2];
+    T v3 = Ms[3];
+    T v4 = Ms[4];
+    T v5 = Ms[5];
+    T v6 = Ms[6];
+    T v7 = Ms[7];
+    T v8 = Ms[8];
+    T v9 = Ms[9];
+    T v10 = Ms[10];
+    T v11 = Ms[11];
+    T v12 = Ms[12];
+    T v13 = Ms[13];
+    T v14 = Ms[14];
+    T v15 = Ms[15];
+    T v16 = Ms[16];
+    T v17 = Ms[17];
+    T v18 = Ms[18];
+    T v19 = Ms[19];
+    T v20 = Ms[20];
+    T v21 = Ms[21];
+    T v22 = Ms[22];
+    T v23 = Ms[23];
+    T v24 = Ms[24];
+    T v25 = Ms[25];
+    T v26 = Ms[26];
+    T v27 = Ms[27];
+    T v28 = Ms[28];
+    T v29 = Ms[29];
+    T v30 = Ms[30];
+    T v31 = Ms[31];
+    T v32 = Ms[32];
+    T v33 = Ms[33];
+    T v34 = Ms[34];
+    T v35 = Ms[35];
+    T v36 = Ms[36];
+    T v37 = Ms[37];
+    T v38 = Ms[38];
+    T v39 = Ms[39];
+    T v40 = Ms[40];
+    T v41 = Ms[41];
+    T v42 = Ms[42];
+    T v43 = Ms[43];
+    T v44 = Ms[44];
+    T v45 = Ms[45];
+    T v46 = Ms[46];
+    T v47 = Ms[47];
+    T v48 = Ms[48];
+    T v49 = Ms[49];
+    T v50 = Ms[50];
+    T v51 = Ms[51];
+    T v52 = Ms[52];
+    T v53 = Ms[53];
+    T v54 = Ms[54];
+    T v55 = Ms[55];
     v44 -= v55;
     v53 -= v55;
     v25 -= v34;
@@ -13641,219 +13641,218 @@ __device__ __forceinline__ void m2l_reduce_moments_h_5(const float *__restrict__
     Mr[35] = v51;
 }
 
-__device__ __forceinline__ void m2l_complete_locals_h_5(const float *__restrict__ Lr, float *__restrict__ L)
+template <class T> __device__ __forceinline__ void m2l_complete_locals_h_5(const T *__restrict__ Lr, T *__restrict__ L)
 {
-    const float v0 = Lr[0];
+    const T v0 = Lr[0];
     L[0] = v0;
-    const float v1 = Lr[1];
+    const T v1 = Lr[1];
     L[1] = v1;
-    const float v2 = Lr[2];
+    const T v2 = Lr[2];
     L[2] = v2;
-    const float v3 = Lr[3];
+    const T v3 = Lr[3];
     L[3] = v3;
-    const float v4 = Lr[4];
+    const T v4 = Lr[4];
     L[4] = v4;
-    const float v5 = Lr[5];
+    const T v5 = Lr[5];
     L[5] = v5;
-    const float v6 = Lr[6];
+    const T v6 = Lr[6];
     L[6] = v6;
-    const float v7 = Lr[7];
+    const T v7 = Lr[7];
     L[7] = v7;
-    const float v8 = Lr[8];
+    const T v8 = Lr[8];
     L[8] = v8;
-    const float v9 = -v4 - v7;
+    const T v9 = -v4 - v7;
     L[9] = v9;
-    const float v10 = Lr[9];
+    const T v10 = Lr[9];
     L[10] = v10;
-    const float v11 = Lr[10];
+    const T v11 = Lr[10];
     L[11] = v11;
-    const float v12 = Lr[11];
+    const T v12 = Lr[11];
     L[12] = v12;
-    const float v13 = Lr[12];
+    const T v13 = Lr[12];
     L[13] = v13;
-    const float v14 = Lr[13];
+    const T v14 = Lr[13];
     L[14] = v14;
-    const float v15 = -v10 - v13;
+    const T v15 = -v10 - v13;
     L[15] = v15;
-    const float v16 = Lr[14];
+    const T v16 = Lr[14];
     L[16] = v16;
-    const float v17 = Lr[15];
+    const T v17 = Lr[15];
     L[17] = v17;
-    const float v18 = -v11 - v16;
+    const T v18 = -v11 - v16;
     L[18] = v18;
-    const float v19 = -v12 - v17;
+    const T v19 = -v12 - v17;
     L[19] = v19;
-    const float v20 = Lr[16];
+    const T v20 = Lr[16];
     L[20] = v20;
-    const float v21 = Lr[17];
+    const T v21 = Lr[17];
     L[21] = v21;
-    const float v22 = Lr[18];
+    const T v22 = Lr[18];
     L[22] = v22;
-    const float v23 = Lr[19];
+    const T v23 = Lr[19];
     L[23] = v23;
-    const float v24 = Lr[20];
+    const T v24 = Lr[20];
     L[24] = v24;
-    const float v25 = -v20 - v23;
+    const T v25 = -v20 - v23;
     L[25] = v25;
-    const float v26 = Lr[21];
+    const T v26 = Lr[21];
     L[26] = v26;
-    const float v27 = Lr[22];
+    const T v27 = Lr[22];
     L[27] = v27;
-    const float v28 = -v21 - v26;
+    const T v28 = -v21 - v26;
     L[28] = v28;
-    const float v29 = -v22 - v27;
+    const T v29 = -v22 - v27;
     L[29] = v29;
-    const float v30 = Lr[23];
+    const T v30 = Lr[23];
     L[30] = v30;
-    const float v31 = Lr[24];
+    const T v31 = Lr[24];
     L[31] = v31;
-    const float v32 = -v23 - v30;
+    const T v32 = -v23 - v30;
     L[32] = v32;
-    const float v33 = -v24 - v31;
+    const T v33 = -v24 - v31;
     L[33] = v33;
-    const float v34 = -v25 - v32;
+    const T v34 = -v25 - v32;
     L[34] = v34;
-    const float v35 = Lr[25];
+    const T v35 = Lr[25];
     L[35] = v35;
-    const float v36 = Lr[26];
+    const T v36 = Lr[26];
     L[36] = v36;
-    const float v37 = Lr[27];
+    const T v37 = Lr[27];
     L[37] = v37;
-    const float v38 = Lr[28];
+    const T v38 = Lr[28];
     L[38] = v38;
-    const float v39 = Lr[29];
+    const T v39 = Lr[29];
     L[39] = v39;
-    const float v40 = -v35 - v38;
+    const T v40 = -v35 - v38;
     L[40] = v40;
-    const float v41 = Lr[30];
+    const T v41 = Lr[30];
     L[41] = v41;
-    const float v42 = Lr[31];
+    const T v42 = Lr[31];
     L[42] = v42;
-    const float v43 = -v36 - v41;
+    const T v43 = -v36 - v41;
     L[43] = v43;
-    const float v44 = -v37 - v42;
+    const T v44 = -v37 - v42;
     L[44] = v44;
-    const float v45 = Lr[32];
+    const T v45 = Lr[32];
     L[45] = v45;
-    const float v46 = Lr[33];
+    const T v46 = Lr[33];
     L[46] = v46;
-    const float v47 = -v38 - v45;
+    const T v47 = -v38 - v45;
     L[47] = v47;
-    const float v48 = -v39 - v46;
+    const T v48 = -v39 - v46;
     L[48] = v48;
-    const float v49 = -v40 - v47;
+    const T v49 = -v40 - v47;
     L[49] = v49;
-    const float v50 = Lr[34];
+    const T v50 = Lr[34];
     L[50] = v50;
-    const float v51 = Lr[35];
+    const T v51 = Lr[35];
     L[51] = v51;
-    const float v52 = -v41 - v50;
+    const T v52 = -v41 - v50;
     L[52] = v52;
-    const float v53 = -v42 - v51;
+    const T v53 = -v42 - v51;
     L[53] = v53;
-    const float v54 = -v43 - v52;
+    const T v54 = -v43 - v52;
     L[54] = v54;
-    const float v55 = -v44 - v53;
+    const T v55 = -v44 - v53;
     L[55] = v55;
 }
 
-__device__ __forceinline__ void m2l_dtensor_h_6(float dx, float dy, float dz, float (&D)[64])
+template <class T> __device__ __forceinline__ void m2l_dtensor_h_6(T dx, T dy, T dz, T (&D)[64])
 {
-    const float s2 = fmaf(dx, dx, fmaf(dy, dy, dz * dz));
-    float si = rsqrtf(s2);
-    si = si * fmaf(-0.5f * s2, si * si, 1.5f);   // one Newton step
-    const float si2 = si * si;
-    const float f0 = -si;
-    const float f1 = -1.0f * f0 * si2;
-    const float f2 = -3.0f * f1 * si2;
-    const float f3 = -5.0f * f2 * si2;
-    const float f4 = -7.0f * f3 * si2;
-    const float f5 = -9.0f * f4 * si2;
-    const float f6 = -11.0f * f5 * si2;
-    const float r_0_0 = f0;
-    const float r_1_0 = f1;
-    const float r_2_0 = f2;
-    const float r_3_0 = f3;
-    const float r_4_0 = f4;
-    const float r_5_0 = f5;
-    const float r_6_0 = f6;
-    const float r_0_1 = dx * r_1_0;
-    const float r_1_1 = dx * r_2_0;
-    const float r_2_1 = dx * r_3_0;
-    const float r_3_1 = dx * r_4_0;
-    const float r_4_1 = dx * r_5_0;
-    const float r_5_1 = dx * r_6_0;
-    const float r_0_2 = dy * r_1_0;
-    const float r_1_2 = dy * r_2_0;
-    const float r_2_2 = dy * r_3_0;
-    const float r_3_2 = dy * r_4_0;
-    const float r_4_2 = dy * r_5_0;
-    const float r_5_2 = dy * r_6_0;
-    const float r_0_4 = fmaf(1.0f, r_1_0, dx * r_1_1);
-    const float r_1_4 = fmaf(1.0f, r_2_0, dx * r_2_1);
-    const float r_2_4 = fmaf(1.0f, r_3_0, dx * r_3_1);
-    const float r_3_4 = fmaf(1.0f, r_4_0, dx * r_4_1);
-    const float r_4_4 = fmaf(1.0f, r_5_0, dx * r_5_1);
-    const float r_0_5 = dx * r_1_2;
-    const float r_1_5 = dx * r_2_2;
-    const float r_2_5 = dx * r_3_2;
-    const float r_3_5 = dx * r_4_2;
-    const float r_4_5 = dx * r_5_2;
-    const float r_0_7 = fmaf(1.0f, r_1_0, dy * r_1_2);
-    const float r_1_7 = fmaf(1.0f, r_2_0, dy * r_2_2);
-    const float r_2_7 = fmaf(1.0f, r_3_0, dy * r_3_2);
-    const float r_3_7 = fmaf(1.0f, r_4_0, dy * r_4_2);
-    const float r_4_7 = fmaf(1.0f, r_5_0, dy * r_5_2);
-    const float r_0_10 = fmaf(2.0f, r_1_1, dx * r_1_4);
-    const float r_1_10 = fmaf(2.0f, r_2_1, dx * r_2_4);
-    const float r_2_10 = fmaf(2.0f, r_3_1, dx * r_3_4);
-    const float r_3_10 = fmaf(2.0f, r_4_1, dx * r_4_4);
-    const float r_0_11 = fmaf(1.0f, r_1_2, dx * r_1_5);
-    const float r_1_11 = fmaf(1.0f, r_2_2, dx * r_2_5);
-    const float r_2_11 = fmaf(1.0f, r_3_2, dx * r_3_5);
-    const float r_3_11 = fmaf(1.0f, r_4_2, dx * r_4_5);
-    const float r_0_13 = dx * r_1_7;
-    const float r_1_13 = dx * r_2_7;
-    const float r_2_13 = dx * r_3_7;
-    const float r_3_13 = dx * r_4_7;
-    const float r_0_16 = fmaf(2.0f, r_1_2, dy * r_1_7);
-    const float r_1_16 = fmaf(2.0f, r_2_2, dy * r_2_7);
-    const float r_2_16 = fmaf(2.0f, r_3_2, dy * r_3_7);
-    const float r_3_16 = fmaf(2.0f, r_4_2, dy * r_4_7);
-    const float r_0_20 = fmaf(3.0f, r_1_4, dx * r_1_10);
-    const float r_1_20 = fmaf(3.0f, r_2_4, dx * r_2_10);
-    const float r_2_20 = fmaf(3.0f, r_3_4, dx * r_3_10);
-    const float r_0_21 = fmaf(2.0f, r_1_5, dx * r_1_11);
-    const float r_1_21 = fmaf(2.0f, r_2_5, dx * r_2_11);
-    const float r_2_21 = fmaf(2.0f, r_3_5, dx * r_3_11);
-    const float r_0_23 = fmaf(1.0f, r_1_7, dx * r_1_13);
-    const float r_1_23 = fmaf(1.0f, r_2_7, dx * r_2_13);
-    const float r_2_23 = fmaf(1.0f, r_3_7, dx * r_3_13);
-    const float r_0_26 = dx * r_1_16;
-    const float r_1_26 = dx * r_2_16;
-    const float r_2_26 = dx * r_3_16;
-    const float r_0_30 = fmaf(3.0f, r_1_7, dy * r_1_16);
-    const float r_1_30 = fmaf(3.0f, r_2_7, dy * r_2_16);
-    const float r_2_30 = fmaf(3.0f, r_3_7, dy * r_3_16);
-    const float r_0_35 = fmaf(4.0f, r_1_10, dx * r_1_20);
-    const float r_1_35 = fmaf(4.0f, r_2_10, dx * r_2_20);
-    const float r_0_36 = fmaf(3.0f, r_1_11, dx * r_1_21);
-    const float r_1_36 = fmaf(3.0f, r_2_11, dx * r_2_21);
-    const float r_0_38 = fmaf(2.0f, r_1_13, dx * r_1_23);
-    const float r_1_38 = fmaf(2.0f, r_2_13, dx * r_2_23);
-    const float r_0_41 = fmaf(1.0f, r_1_16, dx * r_1_26);
-    const float r_1_41 = fmaf(1.0f, r_2_16, dx * r_2_26);
-    const float r_0_45 = dx * r_1_30;
-    const float r_1_45 = dx * r_2_30;
-    const float r_0_50 = fmaf(4.0f, r_1_16, dy * r_1_30);
-    const float r_1_50 = fmaf(4.0f, r_2_16, dy * r_2_30);
-    const float r_0_56 = fmaf(5.0f, r_1_20, dx * r_1_35);
-    const float r_0_57 = fmaf(4.0f, r_1_21, dx * r_1_36);
-    const float r_0_59 = fmaf(3.0f, r_1_23, dx * r_1_38);
-    const float r_0_62 = fmaf(2.0f, r_1_26, dx * r_1_41);
-    const float r_0_66 = fmaf(1.0f, r_1_30, dx * r_1_45);
-    const float r_0_71 = dx * r_1_50;
-    const float r_0_77 = fmaf(5.0f, r_1_30, dy * r_1_50);
+    const T s2 = m2l_fma(dx, dx, m2l_fma(dy, dy, dz * dz));
+    const T si = m2l_rsqrt(s2);
+    const T si2 = si * si;
+    const T f0 = -si;
+    const T f1 = T(-1) * f0 * si2;
+    const T f2 = T(-3) * f1 * si2;
+    const T f3 = T(-5) * f2 * si2;
+    const T f4 = T(-7) * f3 * si2;
+    const T f5 = T(-9) * f4 * si2;
+    const T f6 = T(-11) * f5 * si2;
+    const T r_0_0 = f0;
+    const T r_1_0 = f1;
+    const T r_2_0 = f2;
+    const T r_3_0 = f3;
+    const T r_4_0 = f4;
+    const T r_5_0 = f5;
+    const T r_6_0 = f6;
+    const T r_0_1 = dx * r_1_0;
+    const T r_1_1 = dx * r_2_0;
+    const T r_2_1 = dx * r_3_0;
+    const T r_3_1 = dx * r_4_0;
+    const T r_4_1 = dx * r_5_0;
+    const T r_5_1 = dx * r_6_0;
+    const T r_0_2 = dy * r_1_0;
+    const T r_1_2 = dy * r_2_0;
+    const T r_2_2 = dy * r_3_0;
+    const T r_3_2 = dy * r_4_0;
+    const T r_4_2 = dy * r_5_0;
+    const T r_5_2 = dy * r_6_0;
+    const T r_0_4 = m2l_fma(T(1), r_1_0, dx * r_1_1);
+    const T r_1_4 = m2l_fma(T(1), r_2_0, dx * r_2_1);
+    const T r_2_4 = m2l_fma(T(1), r_3_0, dx * r_3_1);
+    const T r_3_4 = m2l_fma(T(1), r_4_0, dx * r_4_1);
+    const T r_4_4 = m2l_fma(T(1), r_5_0, dx * r_5_1);
+    const T r_0_5 = dx * r_1_2;
+    const T r_1_5 = dx * r_2_2;
+    const T r_2_5 = dx * r_3_2;
+    const T r_3_5 = dx * r_4_2;
+    const T r_4_5 = dx * r_5_2;
+    const T r_0_7 = m2l_fma(T(1), r_1_0, dy * r_1_2);
+    const T r_1_7 = m2l_fma(T(1), r_2_0, dy * r_2_2);
+    const T r_2_7 = m2l_fma(T(1), r_3_0, dy * r_3_2);
+    const T r_3_7 = m2l_fma(T(1), r_4_0, dy * r_4_2);
+    const T r_4_7 = m2l_fma(T(1), r_5_0, dy * r_5_2);
+    const T r_0_10 = m2l_fma(T(2), r_1_1, dx * r_1_4);
+    const T r_1_10 = m2l_fma(T(2), r_2_1, dx * r_2_4);
+    const T r_2_10 = m2l_fma(T(2), r_3_1, dx * r_3_4);
+    const T r_3_10 = m2l_fma(T(2), r_4_1, dx * r_4_4);
+    const T r_0_11 = m2l_fma(T(1), r_1_2, dx * r_1_5);
+    const T r_1_11 = m2l_fma(T(1), r_2_2, dx * r_2_5);
+    const T r_2_11 = m2l_fma(T(1), r_3_2, dx * r_3_5);
+    const T r_3_11 = m2l_fma(T(1), r_4_2, dx * r_4_5);
+    const T r_0_13 = dx * r_1_7;
+    const T r_1_13 = dx * r_2_7;
+    const T r_2_13 = dx * r_3_7;
+    const T r_3_13 = dx * r_4_7;
+    const T r_0_16 = m2l_fma(T(2), r_1_2, dy * r_1_7);
+    const T r_1_16 = m2l_fma(T(2), r_2_2, dy * r_2_7);
+    const T r_2_16 = m2l_fma(T(2), r_3_2, dy * r_3_7);
+    const T r_3_16 = m2l_fma(T(2), r_4_2, dy * r_4_7);
+    const T r_0_20 = m2l_fma(T(3), r_1_4, dx * r_1_10);
+    const T r_1_20 = m2l_fma(T(3), r_2_4, dx * r_2_10);
+    const T r_2_20 = m2l_fma(T(3), r_3_4, dx * r_3_10);
+    const T r_0_21 = m2l_fma(T(2), r_1_5, dx * r_1_11);
+    const T r_1_21 = m2l_fma(T(2), r_2_5, dx * r_2_11);
+    const T r_2_21 = m2l_fma(T(2), r_3_5, dx * r_3_11);
+    const T r_0_23 = m2l_fma(T(1), r_1_7, dx * r_1_13);
+    const T r_1_23 = m2l_fma(T(1), r_2_7, dx * r_2_13);
+    const T r_2_23 = m2l_fma(T(1), r_3_7, dx * r_3_13);
+    const T r_0_26 = dx * r_1_16;
+    const T r_1_26 = dx * r_2_16;
+    const T r_2_26 = dx * r_3_16;
+    const T r_0_30 = m2l_fma(T(3), r_1_7, dy * r_1_16);
+    const T r_1_30 = m2l_fma(T(3), r_2_7, dy * r_2_16);
+    const T r_2_30 = m2l_fma(T(3), r_3_7, dy * r_3_16);
+    const T r_0_35 = m2l_fma(T(4), r_1_10, dx * r_1_20);
+    const T r_1_35 = m2l_fma(T(4), r_2_10, dx * r_2_20);
+    const T r_0_36 = m2l_fma(T(3), r_1_11, dx * r_1_21);
+    const T r_1_36 = m2l_fma(T(3), r_2_11, dx * r_2_21);
+    const T r_0_38 = m2l_fma(T(2), r_1_13, dx * r_1_23);
+    const T r_1_38 = m2l_fma(T(2), r_2_13, dx * r_2_23);
+    const T r_0_41 = m2l_fma(T(1), r_1_16, dx * r_1_26);
+    const T r_1_41 = m2l_fma(T(1), r_2_16, dx * r_2_26);
+    const T r_0_45 = dx * r_1_30;
+    const T r_1_45 = dx * r_2_30;
+    const T r_0_50 = m2l_fma(T(4), r_1_16, dy * r_1_30);
+    const T r_1_50 = m2l_fma(T(4), r_2_16, dy * r_2_30);
+    const T r_0_56 = m2l_fma(T(5), r_1_20, dx * r_1_35);
+    const T r_0_57 = m2l_fma(T(4), r_1_21, dx * r_1_36);
+    const T r_0_59 = m2l_fma(T(3), r_1_23, dx * r_1_38);
+    const T r_0_62 = m2l_fma(T(2), r_1_26, dx * r_1_41);
+    const T r_0_66 = m2l_fma(T(1), r_1_30, dx * r_1_45);
+    const T r_0_71 = dx * r_1_50;
+    const T r_0_77 = m2l_fma(T(5), r_1_30, dy * r_1_50);
     D[0] = r_0_0;
     D[1] = r_0_1;
     D[2] = r_0_2;
@@ -13920,10 +13919,10 @@ __device__ __forceinline__ void m2l_dtensor_h_6(float dx, float dy, float dz, fl
     D[63] = -D[55] - D[61];
 }
 
-__device__ __forceinline__ void m2l_side_a_h_6(const float (&D)[64], const float *__restrict__ Mr, float rho, float (&L)[49])
+template <class T> __device__ __forceinline__ void m2l_side_a_h_6(const T (&D)[64], const T *__restrict__ Mr, T rho, T (&L)[49])
 {
-    float rp = 1.0f;
-    { const float m = __ldg(Mr + 0) * rp;
+    T rp = T(1);
+    { const T m = __ldg(Mr + 0) * rp;
       L[0] = D[0] * m;
       L[1] = D[1] * m;
       L[2] = D[2] * m;
@@ -13975,1236 +13974,1236 @@ __device__ __forceinline__ void m2l_side_a_h_6(const float (&D)[64], const float
       L[48] = D[62] * m;
     }
     rp *= rho;
-    { const float m = -__ldg(Mr + 1) * rp;
-      L[0] = fmaf(D[1], m, L[0]);
-      L[1] = fmaf(D[4], m, L[1]);
-      L[2] = fmaf(D[5], m, L[2]);
-      L[3] = fmaf(D[6], m, L[3]);
-      L[4] = fmaf(D[10], m, L[4]);
-      L[5] = fmaf(D[11], m, L[5]);
-      L[6] = fmaf(D[12], m, L[6]);
-      L[7] = fmaf(D[13], m, L[7]);
-      L[8] = fmaf(D[14], m, L[8]);
-      L[9] = fmaf(D[19], m, L[9]);
-      L[10] = fmaf(D[20], m, L[10]);
-      L[11] = fmaf(D[21], m, L[11]);
-      L[12] = fmaf(D[22], m, L[12]);
-      L[13] = fmaf(D[23], m, L[13]);
-      L[14] = fmaf(D[25], m, L[14]);
-      L[15] = fmaf(D[26], m, L[15]);
-      L[16] = fmaf(D[31], m, L[16]);
-      L[17] = fmaf(D[32], m, L[17]);
-      L[18] = fmaf(D[33], m, L[18]);
-      L[19] = fmaf(D[34], m, L[19]);
-      L[20] = fmaf(D[35], m, L[20]);
-      L[21] = fmaf(D[37], m, L[21]);
-      L[22] = fmaf(D[38], m, L[22]);
-      L[23] = fmaf(D[40], m, L[23]);
-      L[24] = fmaf(D[41], m, L[24]);
-      L[25] = fmaf(D[46], m, L[25]);
-      L[26] = fmaf(D[47], m, L[26]);
-      L[27] = fmaf(D[48], m, L[27]);
-      L[28] = fmaf(D[49], m, L[28]);
-      L[29] = fmaf(D[50], m, L[29]);
-      L[30] = fmaf(D[52], m, L[30]);
-      L[31] = fmaf(D[53], m, L[31]);
-      L[32] = fmaf(D[55], m, L[32]);
-      L[33] = fmaf(D[56], m, L[33]);
-      L[34] = fmaf(D[58], m, L[34]);
-      L[35] = fmaf(D[59], m, L[35]);
+    { const T m = -__ldg(Mr + 1) * rp;
+      L[0] = m2l_fma(D[1], m, L[0]);
+      L[1] = m2l_fma(D[4], m, L[1]);
+      L[2] = m2l_fma(D[5], m, L[2]);
+      L[3] = m2l_fma(D[6], m, L[3]);
+      L[4] = m2l_fma(D[10], m, L[4]);
+      L[5] = m2l_fma(D[11], m, L[5]);
+      L[6] = m2l_fma(D[12], m, L[6]);
+      L[7] = m2l_fma(D[13], m, L[7]);
+      L[8] = m2l_fma(D[14], m, L[8]);
+      L[9] = m2l_fma(D[19], m, L[9]);
+      L[10] = m2l_fma(D[20], m, L[10]);
+      L[11] = m2l_fma(D[21], m, L[11]);
+      L[12] = m2l_fma(D[22], m, L[12]);
+      L[13] = m2l_fma(D[23], m, L[13]);
+      L[14] = m2l_fma(D[25], m, L[14]);
+      L[15] = m2l_fma(D[26], m, L[15]);
+      L[16] = m2l_fma(D[31], m, L[16]);
+      L[17] = m2l_fma(D[32], m, L[17]);
+      L[18] = m2l_fma(D[33], m, L[18]);
+      L[19] = m2l_fma(D[34], m, L[19]);
+      L[20] = m2l_fma(D[35], m, L[20]);
+      L[21] = m2l_fma(D[37], m, L[21]);
+      L[22] = m2l_fma(D[38], m, L[22]);
+      L[23] = m2l_fma(D[40], m, L[23]);
+      L[24] = m2l_fma(D[41], m, L[24]);
+      L[25] = m2l_fma(D[46], m, L[25]);
+      L[26] = m2l_fma(D[47], m, L[26]);
+      L[27] = m2l_fma(D[48], m, L[27]);
+      L[28] = m2l_fma(D[49], m, L[28]);
+      L[29] = m2l_fma(D[50], m, L[29]);
+      L[30] = m2l_fma(D[52], m, L[30]);
+      L[31] = m2l_fma(D[53], m, L[31]);
+      L[32] = m2l_fma(D[55], m, L[32]);
+      L[33] = m2l_fma(D[56], m, L[33]);
+      L[34] = m2l_fma(D[58], m, L[34]);
+      L[35] = m2l_fma(D[59], m, L[35]);
     }
-    { const float m = -__ldg(Mr + 2) * rp;
-      L[0] = fmaf(D[2], m, L[0]);
-      L[1] = fmaf(D[5], m, L[1]);
-      L[2] = fmaf(D[7], m, L[2]);
-      L[3] = fmaf(D[8], m, L[3]);
-      L[4] = fmaf(D[11], m, L[4]);
-      L[5] = fmaf(D[13], m, L[5]);
-      L[6] = fmaf(D[14], m, L[6]);
-      L[7] = fmaf(D[16], m, L[7]);
-      L[8] = fmaf(D[17], m, L[8]);
-      L[9] = fmaf(D[20], m, L[9]);
-      L[10] = fmaf(D[22], m, L[10]);
-      L[11] = fmaf(D[23], m, L[11]);
-      L[12] = fmaf(D[25], m, L[12]);
-      L[13] = fmaf(D[26], m, L[13]);
-      L[14] = fmaf(D[28], m, L[14]);
-      L[15] = fmaf(D[29], m, L[15]);
-      L[16] = fmaf(D[32], m, L[16]);
-      L[17] = fmaf(D[34], m, L[17]);
-      L[18] = fmaf(D[35], m, L[18]);
-      L[19] = fmaf(D[37], m, L[19]);
-      L[20] = fmaf(D[38], m, L[20]);
-      L[21] = fmaf(D[40], m, L[21]);
-      L[22] = fmaf(D[41], m, L[22]);
-      L[23] = fmaf(D[43], m, L[23]);
-      L[24] = fmaf(D[44], m, L[24]);
-      L[25] = fmaf(D[47], m, L[25]);
-      L[26] = fmaf(D[49], m, L[26]);
-      L[27] = fmaf(D[50], m, L[27]);
-      L[28] = fmaf(D[52], m, L[28]);
-      L[29] = fmaf(D[53], m, L[29]);
-      L[30] = fmaf(D[55], m, L[30]);
-      L[31] = fmaf(D[56], m, L[31]);
-      L[32] = fmaf(D[58], m, L[32]);
-      L[33] = fmaf(D[59], m, L[33]);
-      L[34] = fmaf(D[61], m, L[34]);
-      L[35] = fmaf(D[62], m, L[35]);
+    { const T m = -__ldg(Mr + 2) * rp;
+      L[0] = m2l_fma(D[2], m, L[0]);
+      L[1] = m2l_fma(D[5], m, L[1]);
+      L[2] = m2l_fma(D[7], m, L[2]);
+      L[3] = m2l_fma(D[8], m, L[3]);
+      L[4] = m2l_fma(D[11], m, L[4]);
+      L[5] = m2l_fma(D[13], m, L[5]);
+      L[6] = m2l_fma(D[14], m, L[6]);
+      L[7] = m2l_fma(D[16], m, L[7]);
+      L[8] = m2l_fma(D[17], m, L[8]);
+      L[9] = m2l_fma(D[20], m, L[9]);
+      L[10] = m2l_fma(D[22], m, L[10]);
+      L[11] = m2l_fma(D[23], m, L[11]);
+      L[12] = m2l_fma(D[25], m, L[12]);
+      L[13] = m2l_fma(D[26], m, L[13]);
+      L[14] = m2l_fma(D[28], m, L[14]);
+      L[15] = m2l_fma(D[29], m, L[15]);
+      L[16] = m2l_fma(D[32], m, L[16]);
+      L[17] = m2l_fma(D[34], m, L[17]);
+      L[18] = m2l_fma(D[35], m, L[18]);
+      L[19] = m2l_fma(D[37], m, L[19]);
+      L[20] = m2l_fma(D[38], m, L[20]);
+      L[21] = m2l_fma(D[40], m, L[21]);
+      L[22] = m2l_fma(D[41], m, L[22]);
+      L[23] = m2l_fma(D[43], m, L[23]);
+      L[24] = m2l_fma(D[44], m, L[24]);
+      L[25] = m2l_fma(D[47], m, L[25]);
+      L[26] = m2l_fma(D[49], m, L[26]);
+      L[27] = m2l_fma(D[50], m, L[27]);
+      L[28] = m2l_fma(D[52], m, L[28]);
+      L[29] = m2l_fma(D[53], m, L[29]);
+      L[30] = m2l_fma(D[55], m, L[30]);
+      L[31] = m2l_fma(D[56], m, L[31]);
+      L[32] = m2l_fma(D[58], m, L[32]);
+      L[33] = m2l_fma(D[59], m, L[33]);
+      L[34] = m2l_fma(D[61], m, L[34]);
+      L[35] = m2l_fma(D[62], m, L[35]);
     }
-    { const float m = -__ldg(Mr + 3) * rp;
-      L[0] = fmaf(D[3], m, L[0]);
-      L[1] = fmaf(D[6], m, L[1]);
-      L[2] = fmaf(D[8], m, L[2]);
-      L[3] = fmaf(D[9], m, L[3]);
-      L[4] = fmaf(D[12], m, L[4]);
-      L[5] = fmaf(D[14], m, L[5]);
-      L[6] = fmaf(D[15], m, L[6]);
-      L[7] = fmaf(D[17], m, L[7]);
-      L[8] = fmaf(D[18], m, L[8]);
-      L[9] = fmaf(D[21], m, L[9]);
-      L[10] = fmaf(D[23], m, L[10]);
-      L[11] = fmaf(D[24], m, L[11]);
-      L[12] = fmaf(D[26], m, L[12]);
-      L[13] = fmaf(D[27], m, L[13]);
-      L[14] = fmaf(D[29], m, L[14]);
-      L[15] = fmaf(D[30], m, L[15]);
-      L[16] = fmaf(D[33], m, L[16]);
-      L[17] = fmaf(D[35], m, L[17]);
-      L[18] = fmaf(D[36], m, L[18]);
-      L[19] = fmaf(D[38], m, L[19]);
-      L[20] = fmaf(D[39], m, L[20]);
-      L[21] = fmaf(D[41], m, L[21]);
-      L[22] = fmaf(D[42], m, L[22]);
-      L[23] = fmaf(D[44], m, L[23]);
-      L[24] = fmaf(D[45], m, L[24]);
-      L[25] = fmaf(D[48], m, L[25]);
-      L[26] = fmaf(D[50], m, L[26]);
-      L[27] = fmaf(D[51], m, L[27]);
-      L[28] = fmaf(D[53], m, L[28]);
-      L[29] = fmaf(D[54], m, L[29]);
-      L[30] = fmaf(D[56], m, L[30]);
-      L[31] = fmaf(D[57], m, L[31]);
-      L[32] = fmaf(D[59], m, L[32]);
-      L[33] = fmaf(D[60], m, L[33]);
-      L[34] = fmaf(D[62], m, L[34]);
-      L[35] = fmaf(D[63], m, L[35]);
-    }
-    rp *= rho;
-    { const float m = __ldg(Mr + 4) * rp;
-      L[0] = fmaf(D[4], m, L[0]);
-      L[1] = fmaf(D[10], m, L[1]);
-      L[2] = fmaf(D[11], m, L[2]);
-      L[3] = fmaf(D[12], m, L[3]);
-      L[4] = fmaf(D[19], m, L[4]);
-      L[5] = fmaf(D[20], m, L[5]);
-      L[6] = fmaf(D[21], m, L[6]);
-      L[7] = fmaf(D[22], m, L[7]);
-      L[8] = fmaf(D[23], m, L[8]);
-      L[9] = fmaf(D[31], m, L[9]);
-      L[10] = fmaf(D[32], m, L[10]);
-      L[11] = fmaf(D[33], m, L[11]);
-      L[12] = fmaf(D[34], m, L[12]);
-      L[13] = fmaf(D[35], m, L[13]);
-      L[14] = fmaf(D[37], m, L[14]);
-      L[15] = fmaf(D[38], m, L[15]);
-      L[16] = fmaf(D[46], m, L[16]);
-      L[17] = fmaf(D[47], m, L[17]);
-      L[18] = fmaf(D[48], m, L[18]);
-      L[19] = fmaf(D[49], m, L[19]);
-      L[20] = fmaf(D[50], m, L[20]);
-      L[21] = fmaf(D[52], m, L[21]);
-      L[22] = fmaf(D[53], m, L[22]);
-      L[23] = fmaf(D[55], m, L[23]);
-      L[24] = fmaf(D[56], m, L[24]);
-    }
-    { const float m = __ldg(Mr + 5) * rp;
-      L[0] = fmaf(D[5], m, L[0]);
-      L[1] = fmaf(D[11], m, L[1]);
-      L[2] = fmaf(D[13], m, L[2]);
-      L[3] = fmaf(D[14], m, L[3]);
-      L[4] = fmaf(D[20], m, L[4]);
-      L[5] = fmaf(D[22], m, L[5]);
-      L[6] = fmaf(D[23], m, L[6]);
-      L[7] = fmaf(D[25], m, L[7]);
-      L[8] = fmaf(D[26], m, L[8]);
-      L[9] = fmaf(D[32], m, L[9]);
-      L[10] = fmaf(D[34], m, L[10]);
-      L[11] = fmaf(D[35], m, L[11]);
-      L[12] = fmaf(D[37], m, L[12]);
-      L[13] = fmaf(D[38], m, L[13]);
-      L[14] = fmaf(D[40], m, L[14]);
-      L[15] = fmaf(D[41], m, L[15]);
-      L[16] = fmaf(D[47], m, L[16]);
-      L[17] = fmaf(D[49], m, L[17]);
-      L[18] = fmaf(D[50], m, L[18]);
-      L[19] = fmaf(D[52], m, L[19]);
-      L[20] = fmaf(D[53], m, L[20]);
-      L[21] = fmaf(D[55], m, L[21]);
-      L[22] = fmaf(D[56], m, L[22]);
-      L[23] = fmaf(D[58], m, L[23]);
-      L[24] = fmaf(D[59], m, L[24]);
-    }
-    { const float m = __ldg(Mr + 6) * rp;
-      L[0] = fmaf(D[6], m, L[0]);
-      L[1] = fmaf(D[12], m, L[1]);
-      L[2] = fmaf(D[14], m, L[2]);
-      L[3] = fmaf(D[15], m, L[3]);
-      L[4] = fmaf(D[21], m, L[4]);
-      L[5] = fmaf(D[23], m, L[5]);
-      L[6] = fmaf(D[24], m, L[6]);
-      L[7] = fmaf(D[26], m, L[7]);
-      L[8] = fmaf(D[27], m, L[8]);
-      L[9] = fmaf(D[33], m, L[9]);
-      L[10] = fmaf(D[35], m, L[10]);
-      L[11] = fmaf(D[36], m, L[11]);
-      L[12] = fmaf(D[38], m, L[12]);
-      L[13] = fmaf(D[39], m, L[13]);
-      L[14] = fmaf(D[41], m, L[14]);
-      L[15] = fmaf(D[42], m, L[15]);
-      L[16] = fmaf(D[48], m, L[16]);
-      L[17] = fmaf(D[50], m, L[17]);
-      L[18] = fmaf(D[51], m, L[18]);
-      L[19] = fmaf(D[53], m, L[19]);
-      L[20] = fmaf(D[54], m, L[20]);
-      L[21] = fmaf(D[56], m, L[21]);
-      L[22] = fmaf(D[57], m, L[22]);
-      L[23] = fmaf(D[59], m, L[23]);
-      L[24] = fmaf(D[60], m, L[24]);
-    }
-    { const float m = __ldg(Mr + 7) * rp;
-      L[0] = fmaf(D[7], m, L[0]);
-      L[1] = fmaf(D[13], m, L[1]);
-      L[2] = fmaf(D[16], m, L[2]);
-      L[3] = fmaf(D[17], m, L[3]);
-      L[4] = fmaf(D[22], m, L[4]);
-      L[5] = fmaf(D[25], m, L[5]);
-      L[6] = fmaf(D[26], m, L[6]);
-      L[7] = fmaf(D[28], m, L[7]);
-      L[8] = fmaf(D[29], m, L[8]);
-      L[9] = fmaf(D[34], m, L[9]);
-      L[10] = fmaf(D[37], m, L[10]);
-      L[11] = fmaf(D[38], m, L[11]);
-      L[12] = fmaf(D[40], m, L[12]);
-      L[13] = fmaf(D[41], m, L[13]);
-      L[14] = fmaf(D[43], m, L[14]);
-      L[15] = fmaf(D[44], m, L[15]);
-      L[16] = fmaf(D[49], m, L[16]);
-      L[17] = fmaf(D[52], m, L[17]);
-      L[18] = fmaf(D[53], m, L[18]);
-      L[19] = fmaf(D[55], m, L[19]);
-      L[20] = fmaf(D[56], m, L[20]);
-      L[21] = fmaf(D[58], m, L[21]);
-      L[22] = fmaf(D[59], m, L[22]);
-      L[23] = fmaf(D[61], m, L[23]);
-      L[24] = fmaf(D[62], m, L[24]);
-    }
-    { const float m = __ldg(Mr + 8) * rp;
-      L[0] = fmaf(D[8], m, L[0]);
-      L[1] = fmaf(D[14], m, L[1]);
-      L[2] = fmaf(D[17], m, L[2]);
-      L[3] = fmaf(D[18], m, L[3]);
-      L[4] = fmaf(D[23], m, L[4]);
-      L[5] = fmaf(D[26], m, L[5]);
-      L[6] = fmaf(D[27], m, L[6]);
-      L[7] = fmaf(D[29], m, L[7]);
-      L[8] = fmaf(D[30], m, L[8]);
-      L[9] = fmaf(D[35], m, L[9]);
-      L[10] = fmaf(D[38], m, L[10]);
-      L[11] = fmaf(D[39], m, L[11]);
-      L[12] = fmaf(D[41], m, L[12]);
-      L[13] = fmaf(D[42], m, L[13]);
-      L[14] = fmaf(D[44], m, L[14]);
-      L[15] = fmaf(D[45], m, L[15]);
-      L[16] = fmaf(D[50], m, L[16]);
-      L[17] = fmaf(D[53], m, L[17]);
-      L[18] = fmaf(D[54], m, L[18]);
-      L[19] = fmaf(D[56], m, L[19]);
-      L[20] = fmaf(D[57], m, L[20]);
-      L[21] = fmaf(D[59], m, L[21]);
-      L[22] = fmaf(D[60], m, L[22]);
-      L[23] = fmaf(D[62], m, L[23]);
-      L[24] = fmaf(D[63], m, L[24]);
+    { const T m = -__ldg(Mr + 3) * rp;
+      L[0] = m2l_fma(D[3], m, L[0]);
+      L[1] = m2l_fma(D[6], m, L[1]);
+      L[2] = m2l_fma(D[8], m, L[2]);
+      L[3] = m2l_fma(D[9], m, L[3]);
+      L[4] = m2l_fma(D[12], m, L[4]);
+      L[5] = m2l_fma(D[14], m, L[5]);
+      L[6] = m2l_fma(D[15], m, L[6]);
+      L[7] = m2l_fma(D[17], m, L[7]);
+      L[8] = m2l_fma(D[18], m, L[8]);
+      L[9] = m2l_fma(D[21], m, L[9]);
+      L[10] = m2l_fma(D[23], m, L[10]);
+      L[11] = m2l_fma(D[24], m, L[11]);
+      L[12] = m2l_fma(D[26], m, L[12]);
+      L[13] = m2l_fma(D[27], m, L[13]);
+      L[14] = m2l_fma(D[29], m, L[14]);
+      L[15] = m2l_fma(D[30], m, L[15]);
+      L[16] = m2l_fma(D[33], m, L[16]);
+      L[17] = m2l_fma(D[35], m, L[17]);
+      L[18] = m2l_fma(D[36], m, L[18]);
+      L[19] = m2l_fma(D[38], m, L[19]);
+      L[20] = m2l_fma(D[39], m, L[20]);
+      L[21] = m2l_fma(D[41], m, L[21]);
+      L[22] = m2l_fma(D[42], m, L[22]);
+      L[23] = m2l_fma(D[44], m, L[23]);
+      L[24] = m2l_fma(D[45], m, L[24]);
+      L[25] = m2l_fma(D[48], m, L[25]);
+      L[26] = m2l_fma(D[50], m, L[26]);
+      L[27] = m2l_fma(D[51], m, L[27]);
+      L[28] = m2l_fma(D[53], m, L[28]);
+      L[29] = m2l_fma(D[54], m, L[29]);
+      L[30] = m2l_fma(D[56], m, L[30]);
+      L[31] = m2l_fma(D[57], m, L[31]);
+      L[32] = m2l_fma(D[59], m, L[32]);
+      L[33] = m2l_fma(D[60], m, L[33]);
+      L[34] = m2l_fma(D[62], m, L[34]);
+      L[35] = m2l_fma(D[63], m, L[35]);
     }
     rp *= rho;
-    { const float m = -__ldg(Mr + 9) * rp;
-      L[0] = fmaf(D[10], m, L[0]);
-      L[1] = fmaf(D[19], m, L[1]);
-      L[2] = fmaf(D[20], m, L[2]);
-      L[3] = fmaf(D[21], m, L[3]);
-      L[4] = fmaf(D[31], m, L[4]);
-      L[5] = fmaf(D[32], m, L[5]);
-      L[6] = fmaf(D[33], m, L[6]);
-      L[7] = fmaf(D[34], m, L[7]);
-      L[8] = fmaf(D[35], m, L[8]);
-      L[9] = fmaf(D[46], m, L[9]);
-      L[10] = fmaf(D[47], m, L[10]);
-      L[11] = fmaf(D[48], m, L[11]);
-      L[12] = fmaf(D[49], m, L[12]);
-      L[13] = fmaf(D[50], m, L[13]);
-      L[14] = fmaf(D[52], m, L[14]);
-      L[15] = fmaf(D[53], m, L[15]);
+    { const T m = __ldg(Mr + 4) * rp;
+      L[0] = m2l_fma(D[4], m, L[0]);
+      L[1] = m2l_fma(D[10], m, L[1]);
+      L[2] = m2l_fma(D[11], m, L[2]);
+      L[3] = m2l_fma(D[12], m, L[3]);
+      L[4] = m2l_fma(D[19], m, L[4]);
+      L[5] = m2l_fma(D[20], m, L[5]);
+      L[6] = m2l_fma(D[21], m, L[6]);
+      L[7] = m2l_fma(D[22], m, L[7]);
+      L[8] = m2l_fma(D[23], m, L[8]);
+      L[9] = m2l_fma(D[31], m, L[9]);
+      L[10] = m2l_fma(D[32], m, L[10]);
+      L[11] = m2l_fma(D[33], m, L[11]);
+      L[12] = m2l_fma(D[34], m, L[12]);
+      L[13] = m2l_fma(D[35], m, L[13]);
+      L[14] = m2l_fma(D[37], m, L[14]);
+      L[15] = m2l_fma(D[38], m, L[15]);
+      L[16] = m2l_fma(D[46], m, L[16]);
+      L[17] = m2l_fma(D[47], m, L[17]);
+      L[18] = m2l_fma(D[48], m, L[18]);
+      L[19] = m2l_fma(D[49], m, L[19]);
+      L[20] = m2l_fma(D[50], m, L[20]);
+      L[21] = m2l_fma(D[52], m, L[21]);
+      L[22] = m2l_fma(D[53], m, L[22]);
+      L[23] = m2l_fma(D[55], m, L[23]);
+      L[24] = m2l_fma(D[56], m, L[24]);
     }
-    { const float m = -__ldg(Mr + 10) * rp;
-      L[0] = fmaf(D[11], m, L[0]);
-      L[1] = fmaf(D[20], m, L[1]);
-      L[2] = fmaf(D[22], m, L[2]);
-      L[3] = fmaf(D[23], m, L[3]);
-      L[4] = fmaf(D[32], m, L[4]);
-      L[5] = fmaf(D[34], m, L[5]);
-      L[6] = fmaf(D[35], m, L[6]);
-      L[7] = fmaf(D[37], m, L[7]);
-      L[8] = fmaf(D[38], m, L[8]);
-      L[9] = fmaf(D[47], m, L[9]);
-      L[10] = fmaf(D[49], m, L[10]);
-      L[11] = fmaf(D[50], m, L[11]);
-      L[12] = fmaf(D[52], m, L[12]);
-      L[13] = fmaf(D[53], m, L[13]);
-      L[14] = fmaf(D[55], m, L[14]);
-      L[15] = fmaf(D[56], m, L[15]);
+    { const T m = __ldg(Mr + 5) * rp;
+      L[0] = m2l_fma(D[5], m, L[0]);
+      L[1] = m2l_fma(D[11], m, L[1]);
+      L[2] = m2l_fma(D[13], m, L[2]);
+      L[3] = m2l_fma(D[14], m, L[3]);
+      L[4] = m2l_fma(D[20], m, L[4]);
+      L[5] = m2l_fma(D[22], m, L[5]);
+      L[6] = m2l_fma(D[23], m, L[6]);
+      L[7] = m2l_fma(D[25], m, L[7]);
+      L[8] = m2l_fma(D[26], m, L[8]);
+      L[9] = m2l_fma(D[32], m, L[9]);
+      L[10] = m2l_fma(D[34], m, L[10]);
+      L[11] = m2l_fma(D[35], m, L[11]);
+      L[12] = m2l_fma(D[37], m, L[12]);
+      L[13] = m2l_fma(D[38], m, L[13]);
+      L[14] = m2l_fma(D[40], m, L[14]);
+      L[15] = m2l_fma(D[41], m, L[15]);
+      L[16] = m2l_fma(D[47], m, L[16]);
+      L[17] = m2l_fma(D[49], m, L[17]);
+      L[18] = m2l_fma(D[50], m, L[18]);
+      L[19] = m2l_fma(D[52], m, L[19]);
+      L[20] = m2l_fma(D[53], m, L[20]);
+      L[21] = m2l_fma(D[55], m, L[21]);
+      L[22] = m2l_fma(D[56], m, L[22]);
+      L[23] = m2l_fma(D[58], m, L[23]);
+      L[24] = m2l_fma(D[59], m, L[24]);
     }
-    { const float m = -__ldg(Mr + 11) * rp;
-      L[0] = fmaf(D[12], m, L[0]);
-      L[1] = fmaf(D[21], m, L[1]);
-      L[2] = fmaf(D[23], m, L[2]);
-      L[3] = fmaf(D[24], m, L[3]);
-      L[4] = fmaf(D[33], m, L[4]);
-      L[5] = fmaf(D[35], m, L[5]);
-      L[6] = fmaf(D[36], m, L[6]);
-      L[7] = fmaf(D[38], m, L[7]);
-      L[8] = fmaf(D[39], m, L[8]);
-      L[9] = fmaf(D[48], m, L[9]);
-      L[10] = fmaf(D[50], m, L[10]);
-      L[11] = fmaf(D[51], m, L[11]);
-      L[12] = fmaf(D[53], m, L[12]);
-      L[13] = fmaf(D[54], m, L[13]);
-      L[14] = fmaf(D[56], m, L[14]);
-      L[15] = fmaf(D[57], m, L[15]);
+    { const T m = __ldg(Mr + 6) * rp;
+      L[0] = m2l_fma(D[6], m, L[0]);
+      L[1] = m2l_fma(D[12], m, L[1]);
+      L[2] = m2l_fma(D[14], m, L[2]);
+      L[3] = m2l_fma(D[15], m, L[3]);
+      L[4] = m2l_fma(D[21], m, L[4]);
+      L[5] = m2l_fma(D[23], m, L[5]);
+      L[6] = m2l_fma(D[24], m, L[6]);
+      L[7] = m2l_fma(D[26], m, L[7]);
+      L[8] = m2l_fma(D[27], m, L[8]);
+      L[9] = m2l_fma(D[33], m, L[9]);
+      L[10] = m2l_fma(D[35], m, L[10]);
+      L[11] = m2l_fma(D[36], m, L[11]);
+      L[12] = m2l_fma(D[38], m, L[12]);
+      L[13] = m2l_fma(D[39], m, L[13]);
+      L[14] = m2l_fma(D[41], m, L[14]);
+      L[15] = m2l_fma(D[42], m, L[15]);
+      L[16] = m2l_fma(D[48], m, L[16]);
+      L[17] = m2l_fma(D[50], m, L[17]);
+      L[18] = m2l_fma(D[51], m, L[18]);
+      L[19] = m2l_fma(D[53], m, L[19]);
+      L[20] = m2l_fma(D[54], m, L[20]);
+      L[21] = m2l_fma(D[56], m, L[21]);
+      L[22] = m2l_fma(D[57], m, L[22]);
+      L[23] = m2l_fma(D[59], m, L[23]);
+      L[24] = m2l_fma(D[60], m, L[24]);
     }
-    { const float m = -__ldg(Mr + 12) * rp;
-      L[0] = fmaf(D[13], m, L[0]);
-      L[1] = fmaf(D[22], m, L[1]);
-      L[2] = fmaf(D[25], m, L[2]);
-      L[3] = fmaf(D[26], m, L[3]);
-      L[4] = fmaf(D[34], m, L[4]);
-      L[5] = fmaf(D[37], m, L[5]);
-      L[6] = fmaf(D[38], m, L[6]);
-      L[7] = fmaf(D[40], m, L[7]);
-      L[8] = fmaf(D[41], m, L[8]);
-      L[9] = fmaf(D[49], m, L[9]);
-      L[10] = fmaf(D[52], m, L[10]);
-      L[11] = fmaf(D[53], m, L[11]);
-      L[12] = fmaf(D[55], m, L[12]);
-      L[13] = fmaf(D[56], m, L[13]);
-      L[14] = fmaf(D[58], m, L[14]);
-      L[15] = fmaf(D[59], m, L[15]);
+    { const T m = __ldg(Mr + 7) * rp;
+      L[0] = m2l_fma(D[7], m, L[0]);
+      L[1] = m2l_fma(D[13], m, L[1]);
+      L[2] = m2l_fma(D[16], m, L[2]);
+      L[3] = m2l_fma(D[17], m, L[3]);
+      L[4] = m2l_fma(D[22], m, L[4]);
+      L[5] = m2l_fma(D[25], m, L[5]);
+      L[6] = m2l_fma(D[26], m, L[6]);
+      L[7] = m2l_fma(D[28], m, L[7]);
+      L[8] = m2l_fma(D[29], m, L[8]);
+      L[9] = m2l_fma(D[34], m, L[9]);
+      L[10] = m2l_fma(D[37], m, L[10]);
+      L[11] = m2l_fma(D[38], m, L[11]);
+      L[12] = m2l_fma(D[40], m, L[12]);
+      L[13] = m2l_fma(D[41], m, L[13]);
+      L[14] = m2l_fma(D[43], m, L[14]);
+      L[15] = m2l_fma(D[44], m, L[15]);
+      L[16] = m2l_fma(D[49], m, L[16]);
+      L[17] = m2l_fma(D[52], m, L[17]);
+      L[18] = m2l_fma(D[53], m, L[18]);
+      L[19] = m2l_fma(D[55], m, L[19]);
+      L[20] = m2l_fma(D[56], m, L[20]);
+      L[21] = m2l_fma(D[58], m, L[21]);
+      L[22] = m2l_fma(D[59], m, L[22]);
+      L[23] = m2l_fma(D[61], m, L[23]);
+      L[24] = m2l_fma(D[62], m, L[24]);
     }
-    { const float m = -__ldg(Mr + 13) * rp;
-      L[0] = fmaf(D[14], m, L[0]);
-      L[1] = fmaf(D[23], m, L[1]);
-      L[2] = fmaf(D[26], m, L[2]);
-      L[3] = fmaf(D[27], m, L[3]);
-      L[4] = fmaf(D[35], m, L[4]);
-      L[5] = fmaf(D[38], m, L[5]);
-      L[6] = fmaf(D[39], m, L[6]);
-      L[7] = fmaf(D[41], m, L[7]);
-      L[8] = fmaf(D[42], m, L[8]);
-      L[9] = fmaf(D[50], m, L[9]);
-      L[10] = fmaf(D[53], m, L[10]);
-      L[11] = fmaf(D[54], m, L[11]);
-      L[12] = fmaf(D[56], m, L[12]);
-      L[13] = fmaf(D[57], m, L[13]);
-      L[14] = fmaf(D[59], m, L[14]);
-      L[15] = fmaf(D[60], m, L[15]);
-    }
-    { const float m = -__ldg(Mr + 14) * rp;
-      L[0] = fmaf(D[16], m, L[0]);
-      L[1] = fmaf(D[25], m, L[1]);
-      L[2] = fmaf(D[28], m, L[2]);
-      L[3] = fmaf(D[29], m, L[3]);
-      L[4] = fmaf(D[37], m, L[4]);
-      L[5] = fmaf(D[40], m, L[5]);
-      L[6] = fmaf(D[41], m, L[6]);
-      L[7] = fmaf(D[43], m, L[7]);
-      L[8] = fmaf(D[44], m, L[8]);
-      L[9] = fmaf(D[52], m, L[9]);
-      L[10] = fmaf(D[55], m, L[10]);
-      L[11] = fmaf(D[56], m, L[11]);
-      L[12] = fmaf(D[58], m, L[12]);
-      L[13] = fmaf(D[59], m, L[13]);
-      L[14] = fmaf(D[61], m, L[14]);
-      L[15] = fmaf(D[62], m, L[15]);
-    }
-    { const float m = -__ldg(Mr + 15) * rp;
-      L[0] = fmaf(D[17], m, L[0]);
-      L[1] = fmaf(D[26], m, L[1]);
-      L[2] = fmaf(D[29], m, L[2]);
-      L[3] = fmaf(D[30], m, L[3]);
-      L[4] = fmaf(D[38], m, L[4]);
-      L[5] = fmaf(D[41], m, L[5]);
-      L[6] = fmaf(D[42], m, L[6]);
-      L[7] = fmaf(D[44], m, L[7]);
-      L[8] = fmaf(D[45], m, L[8]);
-      L[9] = fmaf(D[53], m, L[9]);
-      L[10] = fmaf(D[56], m, L[10]);
-      L[11] = fmaf(D[57], m, L[11]);
-      L[12] = fmaf(D[59], m, L[12]);
-      L[13] = fmaf(D[60], m, L[13]);
-      L[14] = fmaf(D[62], m, L[14]);
-      L[15] = fmaf(D[63], m, L[15]);
-    }
-    rp *= rho;
-    { const float m = __ldg(Mr + 16) * rp;
-      L[0] = fmaf(D[19], m, L[0]);
-      L[1] = fmaf(D[31], m, L[1]);
-      L[2] = fmaf(D[32], m, L[2]);
-      L[3] = fmaf(D[33], m, L[3]);
-      L[4] = fmaf(D[46], m, L[4]);
-      L[5] = fmaf(D[47], m, L[5]);
-      L[6] = fmaf(D[48], m, L[6]);
-      L[7] = fmaf(D[49], m, L[7]);
-      L[8] = fmaf(D[50], m, L[8]);
-    }
-    { const float m = __ldg(Mr + 17) * rp;
-      L[0] = fmaf(D[20], m, L[0]);
-      L[1] = fmaf(D[32], m, L[1]);
-      L[2] = fmaf(D[34], m, L[2]);
-      L[3] = fmaf(D[35], m, L[3]);
-      L[4] = fmaf(D[47], m, L[4]);
-      L[5] = fmaf(D[49], m, L[5]);
-      L[6] = fmaf(D[50], m, L[6]);
-      L[7] = fmaf(D[52], m, L[7]);
-      L[8] = fmaf(D[53], m, L[8]);
-    }
-    { const float m = __ldg(Mr + 18) * rp;
-      L[0] = fmaf(D[21], m, L[0]);
-      L[1] = fmaf(D[33], m, L[1]);
-      L[2] = fmaf(D[35], m, L[2]);
-      L[3] = fmaf(D[36], m, L[3]);
-      L[4] = fmaf(D[48], m, L[4]);
-      L[5] = fmaf(D[50], m, L[5]);
-      L[6] = fmaf(D[51], m, L[6]);
-      L[7] = fmaf(D[53], m, L[7]);
-      L[8] = fmaf(D[54], m, L[8]);
-    }
-    { const float m = __ldg(Mr + 19) * rp;
-      L[0] = fmaf(D[22], m, L[0]);
-      L[1] = fmaf(D[34], m, L[1]);
-      L[2] = fmaf(D[37], m, L[2]);
-      L[3] = fmaf(D[38], m, L[3]);
-      L[4] = fmaf(D[49], m, L[4]);
-      L[5] = fmaf(D[52], m, L[5]);
-      L[6] = fmaf(D[53], m, L[6]);
-      L[7] = fmaf(D[55], m, L[7]);
-      L[8] = fmaf(D[56], m, L[8]);
-    }
-    { const float m = __ldg(Mr + 20) * rp;
-      L[0] = fmaf(D[23], m, L[0]);
-      L[1] = fmaf(D[35], m, L[1]);
-      L[2] = fmaf(D[38], m, L[2]);
-      L[3] = fmaf(D[39], m, L[3]);
-      L[4] = fmaf(D[50], m, L[4]);
-      L[5] = fmaf(D[53], m, L[5]);
-      L[6] = fmaf(D[54], m, L[6]);
-      L[7] = fmaf(D[56], m, L[7]);
-      L[8] = fmaf(D[57], m, L[8]);
-    }
-    { const float m = __ldg(Mr + 21) * rp;
-      L[0] = fmaf(D[25], m, L[0]);
-      L[1] = fmaf(D[37], m, L[1]);
-      L[2] = fmaf(D[40], m, L[2]);
-      L[3] = fmaf(D[41], m, L[3]);
-      L[4] = fmaf(D[52], m, L[4]);
-      L[5] = fmaf(D[55], m, L[5]);
-      L[6] = fmaf(D[56], m, L[6]);
-      L[7] = fmaf(D[58], m, L[7]);
-      L[8] = fmaf(D[59], m, L[8]);
-    }
-    { const float m = __ldg(Mr + 22) * rp;
-      L[0] = fmaf(D[26], m, L[0]);
-      L[1] = fmaf(D[38], m, L[1]);
-      L[2] = fmaf(D[41], m, L[2]);
-      L[3] = fmaf(D[42], m, L[3]);
-      L[4] = fmaf(D[53], m, L[4]);
-      L[5] = fmaf(D[56], m, L[5]);
-      L[6] = fmaf(D[57], m, L[6]);
-      L[7] = fmaf(D[59], m, L[7]);
-      L[8] = fmaf(D[60], m, L[8]);
-    }
-    { const float m = __ldg(Mr + 23) * rp;
-      L[0] = fmaf(D[28], m, L[0]);
-      L[1] = fmaf(D[40], m, L[1]);
-      L[2] = fmaf(D[43], m, L[2]);
-      L[3] = fmaf(D[44], m, L[3]);
-      L[4] = fmaf(D[55], m, L[4]);
-      L[5] = fmaf(D[58], m, L[5]);
-      L[6] = fmaf(D[59], m, L[6]);
-      L[7] = fmaf(D[61], m, L[7]);
-      L[8] = fmaf(D[62], m, L[8]);
-    }
-    { const float m = __ldg(Mr + 24) * rp;
-      L[0] = fmaf(D[29], m, L[0]);
-      L[1] = fmaf(D[41], m, L[1]);
-      L[2] = fmaf(D[44], m, L[2]);
-      L[3] = fmaf(D[45], m, L[3]);
-      L[4] = fmaf(D[56], m, L[4]);
-      L[5] = fmaf(D[59], m, L[5]);
-      L[6] = fmaf(D[60], m, L[6]);
-      L[7] = fmaf(D[62], m, L[7]);
-      L[8] = fmaf(D[63], m, L[8]);
+    { const T m = __ldg(Mr + 8) * rp;
+      L[0] = m2l_fma(D[8], m, L[0]);
+      L[1] = m2l_fma(D[14], m, L[1]);
+      L[2] = m2l_fma(D[17], m, L[2]);
+      L[3] = m2l_fma(D[18], m, L[3]);
+      L[4] = m2l_fma(D[23], m, L[4]);
+      L[5] = m2l_fma(D[26], m, L[5]);
+      L[6] = m2l_fma(D[27], m, L[6]);
+      L[7] = m2l_fma(D[29], m, L[7]);
+      L[8] = m2l_fma(D[30], m, L[8]);
+      L[9] = m2l_fma(D[35], m, L[9]);
+      L[10] = m2l_fma(D[38], m, L[10]);
+      L[11] = m2l_fma(D[39], m, L[11]);
+      L[12] = m2l_fma(D[41], m, L[12]);
+      L[13] = m2l_fma(D[42], m, L[13]);
+      L[14] = m2l_fma(D[44], m, L[14]);
+      L[15] = m2l_fma(D[45], m, L[15]);
+      L[16] = m2l_fma(D[50], m, L[16]);
+      L[17] = m2l_fma(D[53], m, L[17]);
+      L[18] = m2l_fma(D[54], m, L[18]);
+      L[19] = m2l_fma(D[56], m, L[19]);
+      L[20] = m2l_fma(D[57], m, L[20]);
+      L[21] = m2l_fma(D[59], m, L[21]);
+      L[22] = m2l_fma(D[60], m, L[22]);
+      L[23] = m2l_fma(D[62], m, L[23]);
+      L[24] = m2l_fma(D[63], m, L[24]);
     }
     rp *= rho;
-    { const float m = -__ldg(Mr + 25) * rp;
-      L[0] = fmaf(D[31], m, L[0]);
-      L[1] = fmaf(D[46], m, L[1]);
-      L[2] = fmaf(D[47], m, L[2]);
-      L[3] = fmaf(D[48], m, L[3]);
+    { const T m = -__ldg(Mr + 9) * rp;
+      L[0] = m2l_fma(D[10], m, L[0]);
+      L[1] = m2l_fma(D[19], m, L[1]);
+      L[2] = m2l_fma(D[20], m, L[2]);
+      L[3] = m2l_fma(D[21], m, L[3]);
+      L[4] = m2l_fma(D[31], m, L[4]);
+      L[5] = m2l_fma(D[32], m, L[5]);
+      L[6] = m2l_fma(D[33], m, L[6]);
+      L[7] = m2l_fma(D[34], m, L[7]);
+      L[8] = m2l_fma(D[35], m, L[8]);
+      L[9] = m2l_fma(D[46], m, L[9]);
+      L[10] = m2l_fma(D[47], m, L[10]);
+      L[11] = m2l_fma(D[48], m, L[11]);
+      L[12] = m2l_fma(D[49], m, L[12]);
+      L[13] = m2l_fma(D[50], m, L[13]);
+      L[14] = m2l_fma(D[52], m, L[14]);
+      L[15] = m2l_fma(D[53], m, L[15]);
     }
-    { const float m = -__ldg(Mr + 26) * rp;
-      L[0] = fmaf(D[32], m, L[0]);
-      L[1] = fmaf(D[47], m, L[1]);
-      L[2] = fmaf(D[49], m, L[2]);
-      L[3] = fmaf(D[50], m, L[3]);
+    { const T m = -__ldg(Mr + 10) * rp;
+      L[0] = m2l_fma(D[11], m, L[0]);
+      L[1] = m2l_fma(D[20], m, L[1]);
+      L[2] = m2l_fma(D[22], m, L[2]);
+      L[3] = m2l_fma(D[23], m, L[3]);
+      L[4] = m2l_fma(D[32], m, L[4]);
+      L[5] = m2l_fma(D[34], m, L[5]);
+      L[6] = m2l_fma(D[35], m, L[6]);
+      L[7] = m2l_fma(D[37], m, L[7]);
+      L[8] = m2l_fma(D[38], m, L[8]);
+      L[9] = m2l_fma(D[47], m, L[9]);
+      L[10] = m2l_fma(D[49], m, L[10]);
+      L[11] = m2l_fma(D[50], m, L[11]);
+      L[12] = m2l_fma(D[52], m, L[12]);
+      L[13] = m2l_fma(D[53], m, L[13]);
+      L[14] = m2l_fma(D[55], m, L[14]);
+      L[15] = m2l_fma(D[56], m, L[15]);
     }
-    { const float m = -__ldg(Mr + 27) * rp;
-      L[0] = fmaf(D[33], m, L[0]);
-      L[1] = fmaf(D[48], m, L[1]);
-      L[2] = fmaf(D[50], m, L[2]);
-      L[3] = fmaf(D[51], m, L[3]);
+    { const T m = -__ldg(Mr + 11) * rp;
+      L[0] = m2l_fma(D[12], m, L[0]);
+      L[1] = m2l_fma(D[21], m, L[1]);
+      L[2] = m2l_fma(D[23], m, L[2]);
+      L[3] = m2l_fma(D[24], m, L[3]);
+      L[4] = m2l_fma(D[33], m, L[4]);
+      L[5] = m2l_fma(D[35], m, L[5]);
+      L[6] = m2l_fma(D[36], m, L[6]);
+      L[7] = m2l_fma(D[38], m, L[7]);
+      L[8] = m2l_fma(D[39], m, L[8]);
+      L[9] = m2l_fma(D[48], m, L[9]);
+      L[10] = m2l_fma(D[50], m, L[10]);
+      L[11] = m2l_fma(D[51], m, L[11]);
+      L[12] = m2l_fma(D[53], m, L[12]);
+      L[13] = m2l_fma(D[54], m, L[13]);
+      L[14] = m2l_fma(D[56], m, L[14]);
+      L[15] = m2l_fma(D[57], m, L[15]);
     }
-    { const float m = -__ldg(Mr + 28) * rp;
-      L[0] = fmaf(D[34], m, L[0]);
-      L[1] = fmaf(D[49], m, L[1]);
-      L[2] = fmaf(D[52], m, L[2]);
-      L[3] = fmaf(D[53], m, L[3]);
+    { const T m = -__ldg(Mr + 12) * rp;
+      L[0] = m2l_fma(D[13], m, L[0]);
+      L[1] = m2l_fma(D[22], m, L[1]);
+      L[2] = m2l_fma(D[25], m, L[2]);
+      L[3] = m2l_fma(D[26], m, L[3]);
+      L[4] = m2l_fma(D[34], m, L[4]);
+      L[5] = m2l_fma(D[37], m, L[5]);
+      L[6] = m2l_fma(D[38], m, L[6]);
+      L[7] = m2l_fma(D[40], m, L[7]);
+      L[8] = m2l_fma(D[41], m, L[8]);
+      L[9] = m2l_fma(D[49], m, L[9]);
+      L[10] = m2l_fma(D[52], m, L[10]);
+      L[11] = m2l_fma(D[53], m, L[11]);
+      L[12] = m2l_fma(D[55], m, L[12]);
+      L[13] = m2l_fma(D[56], m, L[13]);
+      L[14] = m2l_fma(D[58], m, L[14]);
+      L[15] = m2l_fma(D[59], m, L[15]);
     }
-    { const float m = -__ldg(Mr + 29) * rp;
-      L[0] = fmaf(D[35], m, L[0]);
-      L[1] = fmaf(D[50], m, L[1]);
-      L[2] = fmaf(D[53], m, L[2]);
-      L[3] = fmaf(D[54], m, L[3]);
+    { const T m = -__ldg(Mr + 13) * rp;
+      L[0] = m2l_fma(D[14], m, L[0]);
+      L[1] = m2l_fma(D[23], m, L[1]);
+      L[2] = m2l_fma(D[26], m, L[2]);
+      L[3] = m2l_fma(D[27], m, L[3]);
+      L[4] = m2l_fma(D[35], m, L[4]);
+      L[5] = m2l_fma(D[38], m, L[5]);
+      L[6] = m2l_fma(D[39], m, L[6]);
+      L[7] = m2l_fma(D[41], m, L[7]);
+      L[8] = m2l_fma(D[42], m, L[8]);
+      L[9] = m2l_fma(D[50], m, L[9]);
+      L[10] = m2l_fma(D[53], m, L[10]);
+      L[11] = m2l_fma(D[54], m, L[11]);
+      L[12] = m2l_fma(D[56], m, L[12]);
+      L[13] = m2l_fma(D[57], m, L[13]);
+      L[14] = m2l_fma(D[59], m, L[14]);
+      L[15] = m2l_fma(D[60], m, L[15]);
     }
-    { const float m = -__ldg(Mr + 30) * rp;
-      L[0] = fmaf(D[37], m, L[0]);
-      L[1] = fmaf(D[52], m, L[1]);
-      L[2] = fmaf(D[55], m, L[2]);
-      L[3] = fmaf(D[56], m, L[3]);
+    { const T m = -__ldg(Mr + 14) * rp;
+      L[0] = m2l_fma(D[16], m, L[0]);
+      L[1] = m2l_fma(D[25], m, L[1]);
+      L[2] = m2l_fma(D[28], m, L[2]);
+      L[3] = m2l_fma(D[29], m, L[3]);
+      L[4] = m2l_fma(D[37], m, L[4]);
+      L[5] = m2l_fma(D[40], m, L[5]);
+      L[6] = m2l_fma(D[41], m, L[6]);
+      L[7] = m2l_fma(D[43], m, L[7]);
+      L[8] = m2l_fma(D[44], m, L[8]);
+      L[9] = m2l_fma(D[52], m, L[9]);
+      L[10] = m2l_fma(D[55], m, L[10]);
+      L[11] = m2l_fma(D[56], m, L[11]);
+      L[12] = m2l_fma(D[58], m, L[12]);
+      L[13] = m2l_fma(D[59], m, L[13]);
+      L[14] = m2l_fma(D[61], m, L[14]);
+      L[15] = m2l_fma(D[62], m, L[15]);
     }
-    { const float m = -__ldg(Mr + 31) * rp;
-      L[0] = fmaf(D[38], m, L[0]);
-      L[1] = fmaf(D[53], m, L[1]);
-      L[2] = fmaf(D[56], m, L[2]);
-      L[3] = fmaf(D[57], m, L[3]);
-    }
-    { const float m = -__ldg(Mr + 32) * rp;
-      L[0] = fmaf(D[40], m, L[0]);
-      L[1] = fmaf(D[55], m, L[1]);
-      L[2] = fmaf(D[58], m, L[2]);
-      L[3] = fmaf(D[59], m, L[3]);
-    }
-    { const float m = -__ldg(Mr + 33) * rp;
-      L[0] = fmaf(D[41], m, L[0]);
-      L[1] = fmaf(D[56], m, L[1]);
-      L[2] = fmaf(D[59], m, L[2]);
-      L[3] = fmaf(D[60], m, L[3]);
-    }
-    { const float m = -__ldg(Mr + 34) * rp;
-      L[0] = fmaf(D[43], m, L[0]);
-      L[1] = fmaf(D[58], m, L[1]);
-      L[2] = fmaf(D[61], m, L[2]);
-      L[3] = fmaf(D[62], m, L[3]);
-    }
-    { const float m = -__ldg(Mr + 35) * rp;
-      L[0] = fmaf(D[44], m, L[0]);
-      L[1] = fmaf(D[59], m, L[1]);
-      L[2] = fmaf(D[62], m, L[2]);
-      L[3] = fmaf(D[63], m, L[3]);
+    { const T m = -__ldg(Mr + 15) * rp;
+      L[0] = m2l_fma(D[17], m, L[0]);
+      L[1] = m2l_fma(D[26], m, L[1]);
+      L[2] = m2l_fma(D[29], m, L[2]);
+      L[3] = m2l_fma(D[30], m, L[3]);
+      L[4] = m2l_fma(D[38], m, L[4]);
+      L[5] = m2l_fma(D[41], m, L[5]);
+      L[6] = m2l_fma(D[42], m, L[6]);
+      L[7] = m2l_fma(D[44], m, L[7]);
+      L[8] = m2l_fma(D[45], m, L[8]);
+      L[9] = m2l_fma(D[53], m, L[9]);
+      L[10] = m2l_fma(D[56], m, L[10]);
+      L[11] = m2l_fma(D[57], m, L[11]);
+      L[12] = m2l_fma(D[59], m, L[12]);
+      L[13] = m2l_fma(D[60], m, L[13]);
+      L[14] = m2l_fma(D[62], m, L[14]);
+      L[15] = m2l_fma(D[63], m, L[15]);
     }
     rp *= rho;
-    { const float m = __ldg(Mr + 36) * rp;
-      L[0] = fmaf(D[46], m, L[0]);
+    { const T m = __ldg(Mr + 16) * rp;
+      L[0] = m2l_fma(D[19], m, L[0]);
+      L[1] = m2l_fma(D[31], m, L[1]);
+      L[2] = m2l_fma(D[32], m, L[2]);
+      L[3] = m2l_fma(D[33], m, L[3]);
+      L[4] = m2l_fma(D[46], m, L[4]);
+      L[5] = m2l_fma(D[47], m, L[5]);
+      L[6] = m2l_fma(D[48], m, L[6]);
+      L[7] = m2l_fma(D[49], m, L[7]);
+      L[8] = m2l_fma(D[50], m, L[8]);
     }
-    { const float m = __ldg(Mr + 37) * rp;
-      L[0] = fmaf(D[47], m, L[0]);
+    { const T m = __ldg(Mr + 17) * rp;
+      L[0] = m2l_fma(D[20], m, L[0]);
+      L[1] = m2l_fma(D[32], m, L[1]);
+      L[2] = m2l_fma(D[34], m, L[2]);
+      L[3] = m2l_fma(D[35], m, L[3]);
+      L[4] = m2l_fma(D[47], m, L[4]);
+      L[5] = m2l_fma(D[49], m, L[5]);
+      L[6] = m2l_fma(D[50], m, L[6]);
+      L[7] = m2l_fma(D[52], m, L[7]);
+      L[8] = m2l_fma(D[53], m, L[8]);
     }
-    { const float m = __ldg(Mr + 38) * rp;
-      L[0] = fmaf(D[48], m, L[0]);
+    { const T m = __ldg(Mr + 18) * rp;
+      L[0] = m2l_fma(D[21], m, L[0]);
+      L[1] = m2l_fma(D[33], m, L[1]);
+      L[2] = m2l_fma(D[35], m, L[2]);
+      L[3] = m2l_fma(D[36], m, L[3]);
+      L[4] = m2l_fma(D[48], m, L[4]);
+      L[5] = m2l_fma(D[50], m, L[5]);
+      L[6] = m2l_fma(D[51], m, L[6]);
+      L[7] = m2l_fma(D[53], m, L[7]);
+      L[8] = m2l_fma(D[54], m, L[8]);
     }
-    { const float m = __ldg(Mr + 39) * rp;
-      L[0] = fmaf(D[49], m, L[0]);
+    { const T m = __ldg(Mr + 19) * rp;
+      L[0] = m2l_fma(D[22], m, L[0]);
+      L[1] = m2l_fma(D[34], m, L[1]);
+      L[2] = m2l_fma(D[37], m, L[2]);
+      L[3] = m2l_fma(D[38], m, L[3]);
+      L[4] = m2l_fma(D[49], m, L[4]);
+      L[5] = m2l_fma(D[52], m, L[5]);
+      L[6] = m2l_fma(D[53], m, L[6]);
+      L[7] = m2l_fma(D[55], m, L[7]);
+      L[8] = m2l_fma(D[56], m, L[8]);
     }
-    { const float m = __ldg(Mr + 40) * rp;
-      L[0] = fmaf(D[50], m, L[0]);
+    { const T m = __ldg(Mr + 20) * rp;
+      L[0] = m2l_fma(D[23], m, L[0]);
+      L[1] = m2l_fma(D[35], m, L[1]);
+      L[2] = m2l_fma(D[38], m, L[2]);
+      L[3] = m2l_fma(D[39], m, L[3]);
+      L[4] = m2l_fma(D[50], m, L[4]);
+      L[5] = m2l_fma(D[53], m, L[5]);
+      L[6] = m2l_fma(D[54], m, L[6]);
+      L[7] = m2l_fma(D[56], m, L[7]);
+      L[8] = m2l_fma(D[57], m, L[8]);
     }
-    { const float m = __ldg(Mr + 41) * rp;
-      L[0] = fmaf(D[52], m, L[0]);
+    { const T m = __ldg(Mr + 21) * rp;
+      L[0] = m2l_fma(D[25], m, L[0]);
+      L[1] = m2l_fma(D[37], m, L[1]);
+      L[2] = m2l_fma(D[40], m, L[2]);
+      L[3] = m2l_fma(D[41], m, L[3]);
+      L[4] = m2l_fma(D[52], m, L[4]);
+      L[5] = m2l_fma(D[55], m, L[5]);
+      L[6] = m2l_fma(D[56], m, L[6]);
+      L[7] = m2l_fma(D[58], m, L[7]);
+      L[8] = m2l_fma(D[59], m, L[8]);
     }
-    { const float m = __ldg(Mr + 42) * rp;
-      L[0] = fmaf(D[53], m, L[0]);
+    { const T m = __ldg(Mr + 22) * rp;
+      L[0] = m2l_fma(D[26], m, L[0]);
+      L[1] = m2l_fma(D[38], m, L[1]);
+      L[2] = m2l_fma(D[41], m, L[2]);
+      L[3] = m2l_fma(D[42], m, L[3]);
+      L[4] = m2l_fma(D[53], m, L[4]);
+      L[5] = m2l_fma(D[56], m, L[5]);
+      L[6] = m2l_fma(D[57], m, L[6]);
+      L[7] = m2l_fma(D[59], m, L[7]);
+      L[8] = m2l_fma(D[60], m, L[8]);
     }
-    { const float m = __ldg(Mr + 43) * rp;
-      L[0] = fmaf(D[55], m, L[0]);
+    { const T m = __ldg(Mr + 23) * rp;
+      L[0] = m2l_fma(D[28], m, L[0]);
+      L[1] = m2l_fma(D[40], m, L[1]);
+      L[2] = m2l_fma(D[43], m, L[2]);
+      L[3] = m2l_fma(D[44], m, L[3]);
+      L[4] = m2l_fma(D[55], m, L[4]);
+      L[5] = m2l_fma(D[58], m, L[5]);
+      L[6] = m2l_fma(D[59], m, L[6]);
+      L[7] = m2l_fma(D[61], m, L[7]);
+      L[8] = m2l_fma(D[62], m, L[8]);
     }
-    { const float m = __ldg(Mr + 44) * rp;
-      L[0] = fmaf(D[56], m, L[0]);
+    { const T m = __ldg(Mr + 24) * rp;
+      L[0] = m2l_fma(D[29], m, L[0]);
+      L[1] = m2l_fma(D[41], m, L[1]);
+      L[2] = m2l_fma(D[44], m, L[2]);
+      L[3] = m2l_fma(D[45], m, L[3]);
+      L[4] = m2l_fma(D[56], m, L[4]);
+      L[5] = m2l_fma(D[59], m, L[5]);
+      L[6] = m2l_fma(D[60], m, L[6]);
+      L[7] = m2l_fma(D[62], m, L[7]);
+      L[8] = m2l_fma(D[63], m, L[8]);
     }
-    { const float m = __ldg(Mr + 45) * rp;
-      L[0] = fmaf(D[58], m, L[0]);
+    rp *= rho;
+    { const T m = -__ldg(Mr + 25) * rp;
+      L[0] = m2l_fma(D[31], m, L[0]);
+      L[1] = m2l_fma(D[46], m, L[1]);
+      L[2] = m2l_fma(D[47], m, L[2]);
+      L[3] = m2l_fma(D[48], m, L[3]);
     }
-    { const float m = __ldg(Mr + 46) * rp;
-      L[0] = fmaf(D[59], m, L[0]);
+    { const T m = -__ldg(Mr + 26) * rp;
+      L[0] = m2l_fma(D[32], m, L[0]);
+      L[1] = m2l_fma(D[47], m, L[1]);
+      L[2] = m2l_fma(D[49], m, L[2]);
+      L[3] = m2l_fma(D[50], m, L[3]);
     }
-    { const float m = __ldg(Mr + 47) * rp;
-      L[0] = fmaf(D[61], m, L[0]);
+    { const T m = -__ldg(Mr + 27) * rp;
+      L[0] = m2l_fma(D[33], m, L[0]);
+      L[1] = m2l_fma(D[48], m, L[1]);
+      L[2] = m2l_fma(D[50], m, L[2]);
+      L[3] = m2l_fma(D[51], m, L[3]);
     }
-    { const float m = __ldg(Mr + 48) * rp;
-      L[0] = fmaf(D[62], m, L[0]);
+    { const T m = -__ldg(Mr + 28) * rp;
+      L[0] = m2l_fma(D[34], m, L[0]);
+      L[1] = m2l_fma(D[49], m, L[1]);
+      L[2] = m2l_fma(D[52], m, L[2]);
+      L[3] = m2l_fma(D[53], m, L[3]);
+    }
+    { const T m = -__ldg(Mr + 29) * rp;
+      L[0] = m2l_fma(D[35], m, L[0]);
+      L[1] = m2l_fma(D[50], m, L[1]);
+      L[2] = m2l_fma(D[53], m, L[2]);
+      L[3] = m2l_fma(D[54], m, L[3]);
+    }
+    { const T m = -__ldg(Mr + 30) * rp;
+      L[0] = m2l_fma(D[37], m, L[0]);
+      L[1] = m2l_fma(D[52], m, L[1]);
+      L[2] = m2l_fma(D[55], m, L[2]);
+      L[3] = m2l_fma(D[56], m, L[3]);
+    }
+    { const T m = -__ldg(Mr + 31) * rp;
+      L[0] = m2l_fma(D[38], m, L[0]);
+      L[1] = m2l_fma(D[53], m, L[1]);
+      L[2] = m2l_fma(D[56], m, L[2]);
+      L[3] = m2l_fma(D[57], m, L[3]);
+    }
+    { const T m = -__ldg(Mr + 32) * rp;
+      L[0] = m2l_fma(D[40], m, L[0]);
+      L[1] = m2l_fma(D[55], m, L[1]);
+      L[2] = m2l_fma(D[58], m, L[2]);
+      L[3] = m2l_fma(D[59], m, L[3]);
+    }
+    { const T m = -__ldg(Mr + 33) * rp;
+      L[0] = m2l_fma(D[41], m, L[0]);
+      L[1] = m2l_fma(D[56], m, L[1]);
+      L[2] = m2l_fma(D[59], m, L[2]);
+      L[3] = m2l_fma(D[60], m, L[3]);
+    }
+    { const T m = -__ldg(Mr + 34) * rp;
+      L[0] = m2l_fma(D[43], m, L[0]);
+      L[1] = m2l_fma(D[58], m, L[1]);
+      L[2] = m2l_fma(D[61], m, L[2]);
+      L[3] = m2l_fma(D[62], m, L[3]);
+    }
+    { const T m = -__ldg(Mr + 35) * rp;
+      L[0] = m2l_fma(D[44], m, L[0]);
+      L[1] = m2l_fma(D[59], m, L[1]);
+      L[2] = m2l_fma(D[62], m, L[2]);
+      L[3] = m2l_fma(D[63], m, L[3]);
+    }
+    rp *= rho;
+    { const T m = __ldg(Mr + 36) * rp;
+      L[0] = m2l_fma(D[46], m, L[0]);
+    }
+    { const T m = __ldg(Mr + 37) * rp;
+      L[0] = m2l_fma(D[47], m, L[0]);
+    }
+    { const T m = __ldg(Mr + 38) * rp;
+      L[0] = m2l_fma(D[48], m, L[0]);
+    }
+    { const T m = __ldg(Mr + 39) * rp;
+      L[0] = m2l_fma(D[49], m, L[0]);
+    }
+    { const T m = __ldg(Mr + 40) * rp;
+      L[0] = m2l_fma(D[50], m, L[0]);
+    }
+    { const T m = __ldg(Mr + 41) * rp;
+      L[0] = m2l_fma(D[52], m, L[0]);
+    }
+    { const T m = __ldg(Mr + 42) * rp;
+      L[0] = m2l_fma(D[53], m, L[0]);
+    }
+    { const T m = __ldg(Mr + 43) * rp;
+      L[0] = m2l_fma(D[55], m, L[0]);
+    }
+    { const T m = __ldg(Mr + 44) * rp;
+      L[0] = m2l_fma(D[56], m, L[0]);
+    }
+    { const T m = __ldg(Mr + 45) * rp;
+      L[0] = m2l_fma(D[58], m, L[0]);
+    }
+    { const T m = __ldg(Mr + 46) * rp;
+      L[0] = m2l_fma(D[59], m, L[0]);
+    }
+    { const T m = __ldg(Mr + 47) * rp;
+      L[0] = m2l_fma(D[61], m, L[0]);
+    }
+    { const T m = __ldg(Mr + 48) * rp;
+      L[0] = m2l_fma(D[62], m, L[0]);
     }
 }
 
-__device__ __forceinline__ void m2l_acc_h_6(const float (&D)[64], const float *__restrict__ Mr, float rho, float (&L)[49])
+template <class T> __device__ __forceinline__ void m2l_acc_h_6(const T (&D)[64], const T *__restrict__ Mr, T rho, T (&L)[49])
 {
-    float rp = 1.0f;
-    { const float m = __ldg(Mr + 0) * rp;
-      L[0] = fmaf(D[0], m, L[0]);
-      L[1] = fmaf(D[1], m, L[1]);
-      L[2] = fmaf(D[2], m, L[2]);
-      L[3] = fmaf(D[3], m, L[3]);
-      L[4] = fmaf(D[4], m, L[4]);
-      L[5] = fmaf(D[5], m, L[5]);
-      L[6] = fmaf(D[6], m, L[6]);
-      L[7] = fmaf(D[7], m, L[7]);
-      L[8] = fmaf(D[8], m, L[8]);
-      L[9] = fmaf(D[10], m, L[9]);
-      L[10] = fmaf(D[11], m, L[10]);
-      L[11] = fmaf(D[12], m, L[11]);
-      L[12] = fmaf(D[13], m, L[12]);
-      L[13] = fmaf(D[14], m, L[13]);
-      L[14] = fmaf(D[16], m, L[14]);
-      L[15] = fmaf(D[17], m, L[15]);
-      L[16] = fmaf(D[19], m, L[16]);
-      L[17] = fmaf(D[20], m, L[17]);
-      L[18] = fmaf(D[21], m, L[18]);
-      L[19] = fmaf(D[22], m, L[19]);
-      L[20] = fmaf(D[23], m, L[20]);
-      L[21] = fmaf(D[25], m, L[21]);
-      L[22] = fmaf(D[26], m, L[22]);
-      L[23] = fmaf(D[28], m, L[23]);
-      L[24] = fmaf(D[29], m, L[24]);
-      L[25] = fmaf(D[31], m, L[25]);
-      L[26] = fmaf(D[32], m, L[26]);
-      L[27] = fmaf(D[33], m, L[27]);
-      L[28] = fmaf(D[34], m, L[28]);
-      L[29] = fmaf(D[35], m, L[29]);
-      L[30] = fmaf(D[37], m, L[30]);
-      L[31] = fmaf(D[38], m, L[31]);
-      L[32] = fmaf(D[40], m, L[32]);
-      L[33] = fmaf(D[41], m, L[33]);
-      L[34] = fmaf(D[43], m, L[34]);
-      L[35] = fmaf(D[44], m, L[35]);
-      L[36] = fmaf(D[46], m, L[36]);
-      L[37] = fmaf(D[47], m, L[37]);
-      L[38] = fmaf(D[48], m, L[38]);
-      L[39] = fmaf(D[49], m, L[39]);
-      L[40] = fmaf(D[50], m, L[40]);
-      L[41] = fmaf(D[52], m, L[41]);
-      L[42] = fmaf(D[53], m, L[42]);
-      L[43] = fmaf(D[55], m, L[43]);
-      L[44] = fmaf(D[56], m, L[44]);
-      L[45] = fmaf(D[58], m, L[45]);
-      L[46] = fmaf(D[59], m, L[46]);
-      L[47] = fmaf(D[61], m, L[47]);
-      L[48] = fmaf(D[62], m, L[48]);
+    T rp = T(1);
+    { const T m = __ldg(Mr + 0) * rp;
+      L[0] = m2l_fma(D[0], m, L[0]);
+      L[1] = m2l_fma(D[1], m, L[1]);
+      L[2] = m2l_fma(D[2], m, L[2]);
+      L[3] = m2l_fma(D[3], m, L[3]);
+      L[4] = m2l_fma(D[4], m, L[4]);
+      L[5] = m2l_fma(D[5], m, L[5]);
+      L[6] = m2l_fma(D[6], m, L[6]);
+      L[7] = m2l_fma(D[7], m, L[7]);
+      L[8] = m2l_fma(D[8], m, L[8]);
+      L[9] = m2l_fma(D[10], m, L[9]);
+      L[10] = m2l_fma(D[11], m, L[10]);
+      L[11] = m2l_fma(D[12], m, L[11]);
+      L[12] = m2l_fma(D[13], m, L[12]);
+      L[13] = m2l_fma(D[14], m, L[13]);
+      L[14] = m2l_fma(D[16], m, L[14]);
+      L[15] = m2l_fma(D[17], m, L[15]);
+      L[16] = m2l_fma(D[19], m, L[16]);
+      L[17] = m2l_fma(D[20], m, L[17]);
+      L[18] = m2l_fma(D[21], m, L[18]);
+      L[19] = m2l_fma(D[22], m, L[19]);
+      L[20] = m2l_fma(D[23], m, L[20]);
+      L[21] = m2l_fma(D[25], m, L[21]);
+      L[22] = m2l_fma(D[26], m, L[22]);
+      L[23] = m2l_fma(D[28], m, L[23]);
+      L[24] = m2l_fma(D[29], m, L[24]);
+      L[25] = m2l_fma(D[31], m, L[25]);
+      L[26] = m2l_fma(D[32], m, L[26]);
+      L[27] = m2l_fma(D[33], m, L[27]);
+      L[28] = m2l_fma(D[34], m, L[28]);
+      L[29] = m2l_fma(D[35], m, L[29]);
+      L[30] = m2l_fma(D[37], m, L[30]);
+      L[31] = m2l_fma(D[38], m, L[31]);
+      L[32] = m2l_fma(D[40], m, L[32]);
+      L[33] = m2l_fma(D[41], m, L[33]);
+      L[34] = m2l_fma(D[43], m, L[34]);
+      L[35] = m2l_fma(D[44], m, L[35]);
+      L[36] = m2l_fma(D[46], m, L[36]);
+      L[37] = m2l_fma(D[47], m, L[37]);
+      L[38] = m2l_fma(D[48], m, L[38]);
+      L[39] = m2l_fma(D[49], m, L[39]);
+      L[40] = m2l_fma(D[50], m, L[40]);
+      L[41] = m2l_fma(D[52], m, L[41]);
+      L[42] = m2l_fma(D[53], m, L[42]);
+      L[43] = m2l_fma(D[55], m, L[43]);
+      L[44] = m2l_fma(D[56], m, L[44]);
+      L[45] = m2l_fma(D[58], m, L[45]);
+      L[46] = m2l_fma(D[59], m, L[46]);
+      L[47] = m2l_fma(D[61], m, L[47]);
+      L[48] = m2l_fma(D[62], m, L[48]);
     }
     rp *= rho;
-    { const float m = -__ldg(Mr + 1) * rp;
-      L[0] = fmaf(D[1], m, L[0]);
-      L[1] = fmaf(D[4], m, L[1]);
-      L[2] = fmaf(D[5], m, L[2]);
-      L[3] = fmaf(D[6], m, L[3]);
-      L[4] = fmaf(D[10], m, L[4]);
-      L[5] = fmaf(D[11], m, L[5]);
-      L[6] = fmaf(D[12], m, L[6]);
-      L[7] = fmaf(D[13], m, L[7]);
-      L[8] = fmaf(D[14], m, L[8]);
-      L[9] = fmaf(D[19], m, L[9]);
-      L[10] = fmaf(D[20], m, L[10]);
-      L[11] = fmaf(D[21], m, L[11]);
-      L[12] = fmaf(D[22], m, L[12]);
-      L[13] = fmaf(D[23], m, L[13]);
-      L[14] = fmaf(D[25], m, L[14]);
-      L[15] = fmaf(D[26], m, L[15]);
-      L[16] = fmaf(D[31], m, L[16]);
-      L[17] = fmaf(D[32], m, L[17]);
-      L[18] = fmaf(D[33], m, L[18]);
-      L[19] = fmaf(D[34], m, L[19]);
-      L[20] = fmaf(D[35], m, L[20]);
-      L[21] = fmaf(D[37], m, L[21]);
-      L[22] = fmaf(D[38], m, L[22]);
-      L[23] = fmaf(D[40], m, L[23]);
-      L[24] = fmaf(D[41], m, L[24]);
-      L[25] = fmaf(D[46], m, L[25]);
-      L[26] = fmaf(D[47], m, L[26]);
-      L[27] = fmaf(D[48], m, L[27]);
-      L[28] = fmaf(D[49], m, L[28]);
-      L[29] = fmaf(D[50], m, L[29]);
-      L[30] = fmaf(D[52], m, L[30]);
-      L[31] = fmaf(D[53], m, L[31]);
-      L[32] = fmaf(D[55], m, L[32]);
-      L[33] = fmaf(D[56], m, L[33]);
-      L[34] = fmaf(D[58], m, L[34]);
-      L[35] = fmaf(D[59], m, L[35]);
+    { const T m = -__ldg(Mr + 1) * rp;
+      L[0] = m2l_fma(D[1], m, L[0]);
+      L[1] = m2l_fma(D[4], m, L[1]);
+      L[2] = m2l_fma(D[5], m, L[2]);
+      L[3] = m2l_fma(D[6], m, L[3]);
+      L[4] = m2l_fma(D[10], m, L[4]);
+      L[5] = m2l_fma(D[11], m, L[5]);
+      L[6] = m2l_fma(D[12], m, L[6]);
+      L[7] = m2l_fma(D[13], m, L[7]);
+      L[8] = m2l_fma(D[14], m, L[8]);
+      L[9] = m2l_fma(D[19], m, L[9]);
+      L[10] = m2l_fma(D[20], m, L[10]);
+      L[11] = m2l_fma(D[21], m, L[11]);
+      L[12] = m2l_fma(D[22], m, L[12]);
+      L[13] = m2l_fma(D[23], m, L[13]);
+      L[14] = m2l_fma(D[25], m, L[14]);
+      L[15] = m2l_fma(D[26], m, L[15]);
+      L[16] = m2l_fma(D[31], m, L[16]);
+      L[17] = m2l_fma(D[32], m, L[17]);
+      L[18] = m2l_fma(D[33], m, L[18]);
+      L[19] = m2l_fma(D[34], m, L[19]);
+      L[20] = m2l_fma(D[35], m, L[20]);
+      L[21] = m2l_fma(D[37], m, L[21]);
+      L[22] = m2l_fma(D[38], m, L[22]);
+      L[23] = m2l_fma(D[40], m, L[23]);
+      L[24] = m2l_fma(D[41], m, L[24]);
+      L[25] = m2l_fma(D[46], m, L[25]);
+      L[26] = m2l_fma(D[47], m, L[26]);
+      L[27] = m2l_fma(D[48], m, L[27]);
+      L[28] = m2l_fma(D[49], m, L[28]);
+      L[29] = m2l_fma(D[50], m, L[29]);
+      L[30] = m2l_fma(D[52], m, L[30]);
+      L[31] = m2l_fma(D[53], m, L[31]);
+      L[32] = m2l_fma(D[55], m, L[32]);
+      L[33] = m2l_fma(D[56], m, L[33]);
+      L[34] = m2l_fma(D[58], m, L[34]);
+      L[35] = m2l_fma(D[59], m, L[35]);
     }
-    { const float m = -__ldg(Mr + 2) * rp;
-      L[0] = fmaf(D[2], m, L[0]);
-      L[1] = fmaf(D[5], m, L[1]);
-      L[2] = fmaf(D[7], m, L[2]);
-      L[3] = fmaf(D[8], m, L[3]);
-      L[4] = fmaf(D[11], m, L[4]);
-      L[5] = fmaf(D[13], m, L[5]);
-      L[6] = fmaf(D[14], m, L[6]);
-      L[7] = fmaf(D[16], m, L[7]);
-      L[8] = fmaf(D[17], m, L[8]);
-      L[9] = fmaf(D[20], m, L[9]);
-      L[10] = fmaf(D[22], m, L[10]);
-      L[11] = fmaf(D[23], m, L[11]);
-      L[12] = fmaf(D[25], m, L[12]);
-      L[13] = fmaf(D[26], m, L[13]);
-      L[14] = fmaf(D[28], m, L[14]);
-      L[15] = fmaf(D[29], m, L[15]);
-      L[16] = fmaf(D[32], m, L[16]);
-      L[17] = fmaf(D[34], m, L[17]);
-      L[18] = fmaf(D[35], m, L[18]);
-      L[19] = fmaf(D[37], m, L[19]);
-      L[20] = fmaf(D[38], m, L[20]);
-      L[21] = fmaf(D[40], m, L[21]);
-      L[22] = fmaf(D[41], m, L[22]);
-      L[23] = fmaf(D[43], m, L[23]);
-      L[24] = fmaf(D[44], m, L[24]);
-      L[25] = fmaf(D[47], m, L[25]);
-      L[26] = fmaf(D[49], m, L[26]);
-      L[27] = fmaf(D[50], m, L[27]);
-      L[28] = fmaf(D[52], m, L[28]);
-      L[29] = fmaf(D[53], m, L[29]);
-      L[30] = fmaf(D[55], m, L[30]);
-      L[31] = fmaf(D[56], m, L[31]);
-      L[32] = fmaf(D[58], m, L[32]);
-      L[33] = fmaf(D[59], m, L[33]);
-      L[34] = fmaf(D[61], m, L[34]);
-      L[35] = fmaf(D[62], m, L[35]);
+    { const T m = -__ldg(Mr + 2) * rp;
+      L[0] = m2l_fma(D[2], m, L[0]);
+      L[1] = m2l_fma(D[5], m, L[1]);
+      L[2] = m2l_fma(D[7], m, L[2]);
+      L[3] = m2l_fma(D[8], m, L[3]);
+      L[4] = m2l_fma(D[11], m, L[4]);
+      L[5] = m2l_fma(D[13], m, L[5]);
+      L[6] = m2l_fma(D[14], m, L[6]);
+      L[7] = m2l_fma(D[16], m, L[7]);
+      L[8] = m2l_fma(D[17], m, L[8]);
+      L[9] = m2l_fma(D[20], m, L[9]);
+      L[10] = m2l_fma(D[22], m, L[10]);
+      L[11] = m2l_fma(D[23], m, L[11]);
+      L[12] = m2l_fma(D[25], m, L[12]);
+      L[13] = m2l_fma(D[26], m, L[13]);
+      L[14] = m2l_fma(D[28], m, L[14]);
+      L[15] = m2l_fma(D[29], m, L[15]);
+      L[16] = m2l_fma(D[32], m, L[16]);
+      L[17] = m2l_fma(D[34], m, L[17]);
+      L[18] = m2l_fma(D[35], m, L[18]);
+      L[19] = m2l_fma(D[37], m, L[19]);
+      L[20] = m2l_fma(D[38], m, L[20]);
+      L[21] = m2l_fma(D[40], m, L[21]);
+      L[22] = m2l_fma(D[41], m, L[22]);
+      L[23] = m2l_fma(D[43], m, L[23]);
+      L[24] = m2l_fma(D[44], m, L[24]);
+      L[25] = m2l_fma(D[47], m, L[25]);
+      L[26] = m2l_fma(D[49], m, L[26]);
+      L[27] = m2l_fma(D[50], m, L[27]);
+      L[28] = m2l_fma(D[52], m, L[28]);
+      L[29] = m2l_fma(D[53], m, L[29]);
+      L[30] = m2l_fma(D[55], m, L[30]);
+      L[31] = m2l_fma(D[56], m, L[31]);
+      L[32] = m2l_fma(D[58], m, L[32]);
+      L[33] = m2l_fma(D[59], m, L[33]);
+      L[34] = m2l_fma(D[61], m, L[34]);
+      L[35] = m2l_fma(D[62], m, L[35]);
     }
-    { const float m = -__ldg(Mr + 3) * rp;
-      L[0] = fmaf(D[3], m, L[0]);
-      L[1] = fmaf(D[6], m, L[1]);
-      L[2] = fmaf(D[8], m, L[2]);
-      L[3] = fmaf(D[9], m, L[3]);
-      L[4] = fmaf(D[12], m, L[4]);
-      L[5] = fmaf(D[14], m, L[5]);
-      L[6] = fmaf(D[15], m, L[6]);
-      L[7] = fmaf(D[17], m, L[7]);
-      L[8] = fmaf(D[18], m, L[8]);
-      L[9] = fmaf(D[21], m, L[9]);
-      L[10] = fmaf(D[23], m, L[10]);
-      L[11] = fmaf(D[24], m, L[11]);
-      L[12] = fmaf(D[26], m, L[12]);
-      L[13] = fmaf(D[27], m, L[13]);
-      L[14] = fmaf(D[29], m, L[14]);
-      L[15] = fmaf(D[30], m, L[15]);
-      L[16] = fmaf(D[33], m, L[16]);
-      L[17] = fmaf(D[35], m, L[17]);
-      L[18] = fmaf(D[36], m, L[18]);
-      L[19] = fmaf(D[38], m, L[19]);
-      L[20] = fmaf(D[39], m, L[20]);
-      L[21] = fmaf(D[41], m, L[21]);
-      L[22] = fmaf(D[42], m, L[22]);
-      L[23] = fmaf(D[44], m, L[23]);
-      L[24] = fmaf(D[45], m, L[24]);
-      L[25] = fmaf(D[48], m, L[25]);
-      L[26] = fmaf(D[50], m, L[26]);
-      L[27] = fmaf(D[51], m, L[27]);
-      L[28] = fmaf(D[53], m, L[28]);
-      L[29] = fmaf(D[54], m, L[29]);
-      L[30] = fmaf(D[56], m, L[30]);
-      L[31] = fmaf(D[57], m, L[31]);
-      L[32] = fmaf(D[59], m, L[32]);
-      L[33] = fmaf(D[60], m, L[33]);
-      L[34] = fmaf(D[62], m, L[34]);
-      L[35] = fmaf(D[63], m, L[35]);
-    }
-    rp *= rho;
-    { const float m = __ldg(Mr + 4) * rp;
-      L[0] = fmaf(D[4], m, L[0]);
-      L[1] = fmaf(D[10], m, L[1]);
-      L[2] = fmaf(D[11], m, L[2]);
-      L[3] = fmaf(D[12], m, L[3]);
-      L[4] = fmaf(D[19], m, L[4]);
-      L[5] = fmaf(D[20], m, L[5]);
-      L[6] = fmaf(D[21], m, L[6]);
-      L[7] = fmaf(D[22], m, L[7]);
-      L[8] = fmaf(D[23], m, L[8]);
-      L[9] = fmaf(D[31], m, L[9]);
-      L[10] = fmaf(D[32], m, L[10]);
-      L[11] = fmaf(D[33], m, L[11]);
-      L[12] = fmaf(D[34], m, L[12]);
-      L[13] = fmaf(D[35], m, L[13]);
-      L[14] = fmaf(D[37], m, L[14]);
-      L[15] = fmaf(D[38], m, L[15]);
-      L[16] = fmaf(D[46], m, L[16]);
-      L[17] = fmaf(D[47], m, L[17]);
-      L[18] = fmaf(D[48], m, L[18]);
-      L[19] = fmaf(D[49], m, L[19]);
-      L[20] = fmaf(D[50], m, L[20]);
-      L[21] = fmaf(D[52], m, L[21]);
-      L[22] = fmaf(D[53], m, L[22]);
-      L[23] = fmaf(D[55], m, L[23]);
-      L[24] = fmaf(D[56], m, L[24]);
-    }
-    { const float m = __ldg(Mr + 5) * rp;
-      L[0] = fmaf(D[5], m, L[0]);
-      L[1] = fmaf(D[11], m, L[1]);
-      L[2] = fmaf(D[13], m, L[2]);
-      L[3] = fmaf(D[14], m, L[3]);
-      L[4] = fmaf(D[20], m, L[4]);
-      L[5] = fmaf(D[22], m, L[5]);
-      L[6] = fmaf(D[23], m, L[6]);
-      L[7] = fmaf(D[25], m, L[7]);
-      L[8] = fmaf(D[26], m, L[8]);
-      L[9] = fmaf(D[32], m, L[9]);
-      L[10] = fmaf(D[34], m, L[10]);
-      L[11] = fmaf(D[35], m, L[11]);
-      L[12] = fmaf(D[37], m, L[12]);
-      L[13] = fmaf(D[38], m, L[13]);
-      L[14] = fmaf(D[40], m, L[14]);
-      L[15] = fmaf(D[41], m, L[15]);
-      L[16] = fmaf(D[47], m, L[16]);
-      L[17] = fmaf(D[49], m, L[17]);
-      L[18] = fmaf(D[50], m, L[18]);
-      L[19] = fmaf(D[52], m, L[19]);
-      L[20] = fmaf(D[53], m, L[20]);
-      L[21] = fmaf(D[55], m, L[21]);
-      L[22] = fmaf(D[56], m, L[22]);
-      L[23] = fmaf(D[58], m, L[23]);
-      L[24] = fmaf(D[59], m, L[24]);
-    }
-    { const float m = __ldg(Mr + 6) * rp;
-      L[0] = fmaf(D[6], m, L[0]);
-      L[1] = fmaf(D[12], m, L[1]);
-      L[2] = fmaf(D[14], m, L[2]);
-      L[3] = fmaf(D[15], m, L[3]);
-      L[4] = fmaf(D[21], m, L[4]);
-      L[5] = fmaf(D[23], m, L[5]);
-      L[6] = fmaf(D[24], m, L[6]);
-      L[7] = fmaf(D[26], m, L[7]);
-      L[8] = fmaf(D[27], m, L[8]);
-      L[9] = fmaf(D[33], m, L[9]);
-      L[10] = fmaf(D[35], m, L[10]);
-      L[11] = fmaf(D[36], m, L[11]);
-      L[12] = fmaf(D[38], m, L[12]);
-      L[13] = fmaf(D[39], m, L[13]);
-      L[14] = fmaf(D[41], m, L[14]);
-      L[15] = fmaf(D[42], m, L[15]);
-      L[16] = fmaf(D[48], m, L[16]);
-      L[17] = fmaf(D[50], m, L[17]);
-      L[18] = fmaf(D[51], m, L[18]);
-      L[19] = fmaf(D[53], m, L[19]);
-      L[20] = fmaf(D[54], m, L[20]);
-      L[21] = fmaf(D[56], m, L[21]);
-      L[22] = fmaf(D[57], m, L[22]);
-      L[23] = fmaf(D[59], m, L[23]);
-      L[24] = fmaf(D[60], m, L[24]);
-    }
-    { const float m = __ldg(Mr + 7) * rp;
-      L[0] = fmaf(D[7], m, L[0]);
-      L[1] = fmaf(D[13], m, L[1]);
-      L[2] = fmaf(D[16], m, L[2]);
-      L[3] = fmaf(D[17], m, L[3]);
-      L[4] = fmaf(D[22], m, L[4]);
-      L[5] = fmaf(D[25], m, L[5]);
-      L[6] = fmaf(D[26], m, L[6]);
-      L[7] = fmaf(D[28], m, L[7]);
-      L[8] = fmaf(D[29], m, L[8]);
-      L[9] = fmaf(D[34], m, L[9]);
-      L[10] = fmaf(D[37], m, L[10]);
-      L[11] = fmaf(D[38], m, L[11]);
-      L[12] = fmaf(D[40], m, L[12]);
-      L[13] = fmaf(D[41], m, L[13]);
-      L[14] = fmaf(D[43], m, L[14]);
-      L[15] = fmaf(D[44], m, L[15]);
-      L[16] = fmaf(D[49], m, L[16]);
-      L[17] = fmaf(D[52], m, L[17]);
-      L[18] = fmaf(D[53], m, L[18]);
-      L[19] = fmaf(D[55], m, L[19]);
-      L[20] = fmaf(D[56], m, L[20]);
-      L[21] = fmaf(D[58], m, L[21]);
-      L[22] = fmaf(D[59], m, L[22]);
-      L[23] = fmaf(D[61], m, L[23]);
-      L[24] = fmaf(D[62], m, L[24]);
-    }
-    { const float m = __ldg(Mr + 8) * rp;
-      L[0] = fmaf(D[8], m, L[0]);
-      L[1] = fmaf(D[14], m, L[1]);
-      L[2] = fmaf(D[17], m, L[2]);
-      L[3] = fmaf(D[18], m, L[3]);
-      L[4] = fmaf(D[23], m, L[4]);
-      L[5] = fmaf(D[26], m, L[5]);
-      L[6] = fmaf(D[27], m, L[6]);
-      L[7] = fmaf(D[29], m, L[7]);
-      L[8] = fmaf(D[30], m, L[8]);
-      L[9] = fmaf(D[35], m, L[9]);
-      L[10] = fmaf(D[38], m, L[10]);
-      L[11] = fmaf(D[39], m, L[11]);
-      L[12] = fmaf(D[41], m, L[12]);
-      L[13] = fmaf(D[42], m, L[13]);
-      L[14] = fmaf(D[44], m, L[14]);
-      L[15] = fmaf(D[45], m, L[15]);
-      L[16] = fmaf(D[50], m, L[16]);
-      L[17] = fmaf(D[53], m, L[17]);
-      L[18] = fmaf(D[54], m, L[18]);
-      L[19] = fmaf(D[56], m, L[19]);
-      L[20] = fmaf(D[57], m, L[20]);
-      L[21] = fmaf(D[59], m, L[21]);
-      L[22] = fmaf(D[60], m, L[22]);
-      L[23] = fmaf(D[62], m, L[23]);
-      L[24] = fmaf(D[63], m, L[24]);
+    { const T m = -__ldg(Mr + 3) * rp;
+      L[0] = m2l_fma(D[3], m, L[0]);
+      L[1] = m2l_fma(D[6], m, L[1]);
+      L[2] = m2l_fma(D[8], m, L[2]);
+      L[3] = m2l_fma(D[9], m, L[3]);
+      L[4] = m2l_fma(D[12], m, L[4]);
+      L[5] = m2l_fma(D[14], m, L[5]);
+      L[6] = m2l_fma(D[15], m, L[6]);
+      L[7] = m2l_fma(D[17], m, L[7]);
+      L[8] = m2l_fma(D[18], m, L[8]);
+      L[9] = m2l_fma(D[21], m, L[9]);
+      L[10] = m2l_fma(D[23], m, L[10]);
+      L[11] = m2l_fma(D[24], m, L[11]);
+      L[12] = m2l_fma(D[26], m, L[12]);
+      L[13] = m2l_fma(D[27], m, L[13]);
+      L[14] = m2l_fma(D[29], m, L[14]);
+      L[15] = m2l_fma(D[30], m, L[15]);
+      L[16] = m2l_fma(D[33], m, L[16]);
+      L[17] = m2l_fma(D[35], m, L[17]);
+      L[18] = m2l_fma(D[36], m, L[18]);
+      L[19] = m2l_fma(D[38], m, L[19]);
+      L[20] = m2l_fma(D[39], m, L[20]);
+      L[21] = m2l_fma(D[41], m, L[21]);
+      L[22] = m2l_fma(D[42], m, L[22]);
+      L[23] = m2l_fma(D[44], m, L[23]);
+      L[24] = m2l_fma(D[45], m, L[24]);
+      L[25] = m2l_fma(D[48], m, L[25]);
+      L[26] = m2l_fma(D[50], m, L[26]);
+      L[27] = m2l_fma(D[51], m, L[27]);
+      L[28] = m2l_fma(D[53], m, L[28]);
+      L[29] = m2l_fma(D[54], m, L[29]);
+      L[30] = m2l_fma(D[56], m, L[30]);
+      L[31] = m2l_fma(D[57], m, L[31]);
+      L[32] = m2l_fma(D[59], m, L[32]);
+      L[33] = m2l_fma(D[60], m, L[33]);
+      L[34] = m2l_fma(D[62], m, L[34]);
+      L[35] = m2l_fma(D[63], m, L[35]);
     }
     rp *= rho;
-    { const float m = -__ldg(Mr + 9) * rp;
-      L[0] = fmaf(D[10], m, L[0]);
-      L[1] = fmaf(D[19], m, L[1]);
-      L[2] = fmaf(D[20], m, L[2]);
-      L[3] = fmaf(D[21], m, L[3]);
-      L[4] = fmaf(D[31], m, L[4]);
-      L[5] = fmaf(D[32], m, L[5]);
-      L[6] = fmaf(D[33], m, L[6]);
-      L[7] = fmaf(D[34], m, L[7]);
-      L[8] = fmaf(D[35], m, L[8]);
-      L[9] = fmaf(D[46], m, L[9]);
-      L[10] = fmaf(D[47], m, L[10]);
-      L[11] = fmaf(D[48], m, L[11]);
-      L[12] = fmaf(D[49], m, L[12]);
-      L[13] = fmaf(D[50], m, L[13]);
-      L[14] = fmaf(D[52], m, L[14]);
-      L[15] = fmaf(D[53], m, L[15]);
+    { const T m = __ldg(Mr + 4) * rp;
+      L[0] = m2l_fma(D[4], m, L[0]);
+      L[1] = m2l_fma(D[10], m, L[1]);
+      L[2] = m2l_fma(D[11], m, L[2]);
+      L[3] = m2l_fma(D[12], m, L[3]);
+      L[4] = m2l_fma(D[19], m, L[4]);
+      L[5] = m2l_fma(D[20], m, L[5]);
+      L[6] = m2l_fma(D[21], m, L[6]);
+      L[7] = m2l_fma(D[22], m, L[7]);
+      L[8] = m2l_fma(D[23], m, L[8]);
+      L[9] = m2l_fma(D[31], m, L[9]);
+      L[10] = m2l_fma(D[32], m, L[10]);
+      L[11] = m2l_fma(D[33], m, L[11]);
+      L[12] = m2l_fma(D[34], m, L[12]);
+      L[13] = m2l_fma(D[35], m, L[13]);
+      L[14] = m2l_fma(D[37], m, L[14]);
+      L[15] = m2l_fma(D[38], m, L[15]);
+      L[16] = m2l_fma(D[46], m, L[16]);
+      L[17] = m2l_fma(D[47], m, L[17]);
+      L[18] = m2l_fma(D[48], m, L[18]);
+      L[19] = m2l_fma(D[49], m, L[19]);
+      L[20] = m2l_fma(D[50], m, L[20]);
+      L[21] = m2l_fma(D[52], m, L[21]);
+      L[22] = m2l_fma(D[53], m, L[22]);
+      L[23] = m2l_fma(D[55], m, L[23]);
+      L[24] = m2l_fma(D[56], m, L[24]);
     }
-    { const float m = -__ldg(Mr + 10) * rp;
-      L[0] = fmaf(D[11], m, L[0]);
-      L[1] = fmaf(D[20], m, L[1]);
-      L[2] = fmaf(D[22], m, L[2]);
-      L[3] = fmaf(D[23], m, L[3]);
-      L[4] = fmaf(D[32], m, L[4]);
-      L[5] = fmaf(D[34], m, L[5]);
-      L[6] = fmaf(D[35], m, L[6]);
-      L[7] = fmaf(D[37], m, L[7]);
-      L[8] = fmaf(D[38], m, L[8]);
-      L[9] = fmaf(D[47], m, L[9]);
-      L[10] = fmaf(D[49], m, L[10]);
-      L[11] = fmaf(D[50], m, L[11]);
-      L[12] = fmaf(D[52], m, L[12]);
-      L[13] = fmaf(D[53], m, L[13]);
-      L[14] = fmaf(D[55], m, L[14]);
-      L[15] = fmaf(D[56], m, L[15]);
+    { const T m = __ldg(Mr + 5) * rp;
+      L[0] = m2l_fma(D[5], m, L[0]);
+      L[1] = m2l_fma(D[11], m, L[1]);
+      L[2] = m2l_fma(D[13], m, L[2]);
+      L[3] = m2l_fma(D[14], m, L[3]);
+      L[4] = m2l_fma(D[20], m, L[4]);
+      L[5] = m2l_fma(D[22], m, L[5]);
+      L[6] = m2l_fma(D[23], m, L[6]);
+      L[7] = m2l_fma(D[25], m, L[7]);
+      L[8] = m2l_fma(D[26], m, L[8]);
+      L[9] = m2l_fma(D[32], m, L[9]);
+      L[10] = m2l_fma(D[34], m, L[10]);
+      L[11] = m2l_fma(D[35], m, L[11]);
+      L[12] = m2l_fma(D[37], m, L[12]);
+      L[13] = m2l_fma(D[38], m, L[13]);
+      L[14] = m2l_fma(D[40], m, L[14]);
+      L[15] = m2l_fma(D[41], m, L[15]);
+      L[16] = m2l_fma(D[47], m, L[16]);
+      L[17] = m2l_fma(D[49], m, L[17]);
+      L[18] = m2l_fma(D[50], m, L[18]);
+      L[19] = m2l_fma(D[52], m, L[19]);
+      L[20] = m2l_fma(D[53], m, L[20]);
+      L[21] = m2l_fma(D[55], m, L[21]);
+      L[22] = m2l_fma(D[56], m, L[22]);
+      L[23] = m2l_fma(D[58], m, L[23]);
+      L[24] = m2l_fma(D[59], m, L[24]);
     }
-    { const float m = -__ldg(Mr + 11) * rp;
-      L[0] = fmaf(D[12], m, L[0]);
-      L[1] = fmaf(D[21], m, L[1]);
-      L[2] = fmaf(D[23], m, L[2]);
-      L[3] = fmaf(D[24], m, L[3]);
-      L[4] = fmaf(D[33], m, L[4]);
-      L[5] = fmaf(D[35], m, L[5]);
-      L[6] = fmaf(D[36], m, L[6]);
-      L[7] = fmaf(D[38], m, L[7]);
-      L[8] = fmaf(D[39], m, L[8]);
-      L[9] = fmaf(D[48], m, L[9]);
-      L[10] = fmaf(D[50], m, L[10]);
-      L[11] = fmaf(D[51], m, L[11]);
-      L[12] = fmaf(D[53], m, L[12]);
-      L[13] = fmaf(D[54], m, L[13]);
-      L[14] = fmaf(D[56], m, L[14]);
-      L[15] = fmaf(D[57], m, L[15]);
+    { const T m = __ldg(Mr + 6) * rp;
+      L[0] = m2l_fma(D[6], m, L[0]);
+      L[1] = m2l_fma(D[12], m, L[1]);
+      L[2] = m2l_fma(D[14], m, L[2]);
+      L[3] = m2l_fma(D[15], m, L[3]);
+      L[4] = m2l_fma(D[21], m, L[4]);
+      L[5] = m2l_fma(D[23], m, L[5]);
+      L[6] = m2l_fma(D[24], m, L[6]);
+      L[7] = m2l_fma(D[26], m, L[7]);
+      L[8] = m2l_fma(D[27], m, L[8]);
+      L[9] = m2l_fma(D[33], m, L[9]);
+      L[10] = m2l_fma(D[35], m, L[10]);
+      L[11] = m2l_fma(D[36], m, L[11]);
+      L[12] = m2l_fma(D[38], m, L[12]);
+      L[13] = m2l_fma(D[39], m, L[13]);
+      L[14] = m2l_fma(D[41], m, L[14]);
+      L[15] = m2l_fma(D[42], m, L[15]);
+      L[16] = m2l_fma(D[48], m, L[16]);
+      L[17] = m2l_fma(D[50], m, L[17]);
+      L[18] = m2l_fma(D[51], m, L[18]);
+      L[19] = m2l_fma(D[53], m, L[19]);
+      L[20] = m2l_fma(D[54], m, L[20]);
+      L[21] = m2l_fma(D[56], m, L[21]);
+      L[22] = m2l_fma(D[57], m, L[22]);
+      L[23] = m2l_fma(D[59], m, L[23]);
+      L[24] = m2l_fma(D[60], m, L[24]);
     }
-    { const float m = -__ldg(Mr + 12) * rp;
-      L[0] = fmaf(D[13], m, L[0]);
-      L[1] = fmaf(D[22], m, L[1]);
-      L[2] = fmaf(D[25], m, L[2]);
-      L[3] = fmaf(D[26], m, L[3]);
-      L[4] = fmaf(D[34], m, L[4]);
-      L[5] = fmaf(D[37], m, L[5]);
-      L[6] = fmaf(D[38], m, L[6]);
-      L[7] = fmaf(D[40], m, L[7]);
-      L[8] = fmaf(D[41], m, L[8]);
-      L[9] = fmaf(D[49], m, L[9]);
-      L[10] = fmaf(D[52], m, L[10]);
-      L[11] = fmaf(D[53], m, L[11]);
-      L[12] = fmaf(D[55], m, L[12]);
-      L[13] = fmaf(D[56], m, L[13]);
-      L[14] = fmaf(D[58], m, L[14]);
-      L[15] = fmaf(D[59], m, L[15]);
+    { const T m = __ldg(Mr + 7) * rp;
+      L[0] = m2l_fma(D[7], m, L[0]);
+      L[1] = m2l_fma(D[13], m, L[1]);
+      L[2] = m2l_fma(D[16], m, L[2]);
+      L[3] = m2l_fma(D[17], m, L[3]);
+      L[4] = m2l_fma(D[22], m, L[4]);
+      L[5] = m2l_fma(D[25], m, L[5]);
+      L[6] = m2l_fma(D[26], m, L[6]);
+      L[7] = m2l_fma(D[28], m, L[7]);
+      L[8] = m2l_fma(D[29], m, L[8]);
+      L[9] = m2l_fma(D[34], m, L[9]);
+      L[10] = m2l_fma(D[37], m, L[10]);
+      L[11] = m2l_fma(D[38], m, L[11]);
+      L[12] = m2l_fma(D[40], m, L[12]);
+      L[13] = m2l_fma(D[41], m, L[13]);
+      L[14] = m2l_fma(D[43], m, L[14]);
+      L[15] = m2l_fma(D[44], m, L[15]);
+      L[16] = m2l_fma(D[49], m, L[16]);
+      L[17] = m2l_fma(D[52], m, L[17]);
+      L[18] = m2l_fma(D[53], m, L[18]);
+      L[19] = m2l_fma(D[55], m, L[19]);
+      L[20] = m2l_fma(D[56], m, L[20]);
+      L[21] = m2l_fma(D[58], m, L[21]);
+      L[22] = m2l_fma(D[59], m, L[22]);
+      L[23] = m2l_fma(D[61], m, L[23]);
+      L[24] = m2l_fma(D[62], m, L[24]);
     }
-    { const float m = -__ldg(Mr + 13) * rp;
-      L[0] = fmaf(D[14], m, L[0]);
-      L[1] = fmaf(D[23], m, L[1]);
-      L[2] = fmaf(D[26], m, L[2]);
-      L[3] = fmaf(D[27], m, L[3]);
-      L[4] = fmaf(D[35], m, L[4]);
-      L[5] = fmaf(D[38], m, L[5]);
-      L[6] = fmaf(D[39], m, L[6]);
-      L[7] = fmaf(D[41], m, L[7]);
-      L[8] = fmaf(D[42], m, L[8]);
-      L[9] = fmaf(D[50], m, L[9]);
-      L[10] = fmaf(D[53], m, L[10]);
-      L[11] = fmaf(D[54], m, L[11]);
-      L[12] = fmaf(D[56], m, L[12]);
-      L[13] = fmaf(D[57], m, L[13]);
-      L[14] = fmaf(D[59], m, L[14]);
-      L[15] = fmaf(D[60], m, L[15]);
-    }
-    { const float m = -__ldg(Mr + 14) * rp;
-      L[0] = fmaf(D[16], m, L[0]);
-      L[1] = fmaf(D[25], m, L[1]);
-      L[2] = fmaf(D[28], m, L[2]);
-      L[3] = fmaf(D[29], m, L[3]);
-      L[4] = fmaf(D[37], m, L[4]);
-      L[5] = fmaf(D[40], m, L[5]);
-      L[6] = fmaf(D[41], m, L[6]);
-      L[7] = fmaf(D[43], m, L[7]);
-      L[8] = fmaf(D[44], m, L[8]);
-      L[9] = fmaf(D[52], m, L[9]);
-      L[10] = fmaf(D[55], m, L[10]);
-      L[11] = fmaf(D[56], m, L[11]);
-      L[12] = fmaf(D[58], m, L[12]);
-      L[13] = fmaf(D[59], m, L[13]);
-      L[14] = fmaf(D[61], m, L[14]);
-      L[15] = fmaf(D[62], m, L[15]);
-    }
-    { const float m = -__ldg(Mr + 15) * rp;
-      L[0] = fmaf(D[17], m, L[0]);
-      L[1] = fmaf(D[26], m, L[1]);
-      L[2] = fmaf(D[29], m, L[2]);
-      L[3] = fmaf(D[30], m, L[3]);
-      L[4] = fmaf(D[38], m, L[4]);
-      L[5] = fmaf(D[41], m, L[5]);
-      L[6] = fmaf(D[42], m, L[6]);
-      L[7] = fmaf(D[44], m, L[7]);
-      L[8] = fmaf(D[45], m, L[8]);
-      L[9] = fmaf(D[53], m, L[9]);
-      L[10] = fmaf(D[56], m, L[10]);
-      L[11] = fmaf(D[57], m, L[11]);
-      L[12] = fmaf(D[59], m, L[12]);
-      L[13] = fmaf(D[60], m, L[13]);
-      L[14] = fmaf(D[62], m, L[14]);
-      L[15] = fmaf(D[63], m, L[15]);
-    }
-    rp *= rho;
-    { const float m = __ldg(Mr + 16) * rp;
-      L[0] = fmaf(D[19], m, L[0]);
-      L[1] = fmaf(D[31], m, L[1]);
-      L[2] = fmaf(D[32], m, L[2]);
-      L[3] = fmaf(D[33], m, L[3]);
-      L[4] = fmaf(D[46], m, L[4]);
-      L[5] = fmaf(D[47], m, L[5]);
-      L[6] = fmaf(D[48], m, L[6]);
-      L[7] = fmaf(D[49], m, L[7]);
-      L[8] = fmaf(D[50], m, L[8]);
-    }
-    { const float m = __ldg(Mr + 17) * rp;
-      L[0] = fmaf(D[20], m, L[0]);
-      L[1] = fmaf(D[32], m, L[1]);
-      L[2] = fmaf(D[34], m, L[2]);
-      L[3] = fmaf(D[35], m, L[3]);
-      L[4] = fmaf(D[47], m, L[4]);
-      L[5] = fmaf(D[49], m, L[5]);
-      L[6] = fmaf(D[50], m, L[6]);
-      L[7] = fmaf(D[52], m, L[7]);
-      L[8] = fmaf(D[53], m, L[8]);
-    }
-    { const float m = __ldg(Mr + 18) * rp;
-      L[0] = fmaf(D[21], m, L[0]);
-      L[1] = fmaf(D[33], m, L[1]);
-      L[2] = fmaf(D[35], m, L[2]);
-      L[3] = fmaf(D[36], m, L[3]);
-      L[4] = fmaf(D[48], m, L[4]);
-      L[5] = fmaf(D[50], m, L[5]);
-      L[6] = fmaf(D[51], m, L[6]);
-      L[7] = fmaf(D[53], m, L[7]);
-      L[8] = fmaf(D[54], m, L[8]);
-    }
-    { const float m = __ldg(Mr + 19) * rp;
-      L[0] = fmaf(D[22], m, L[0]);
-      L[1] = fmaf(D[34], m, L[1]);
-      L[2] = fmaf(D[37], m, L[2]);
-      L[3] = fmaf(D[38], m, L[3]);
-      L[4] = fmaf(D[49], m, L[4]);
-      L[5] = fmaf(D[52], m, L[5]);
-      L[6] = fmaf(D[53], m, L[6]);
-      L[7] = fmaf(D[55], m, L[7]);
-      L[8] = fmaf(D[56], m, L[8]);
-    }
-    { const float m = __ldg(Mr + 20) * rp;
-      L[0] = fmaf(D[23], m, L[0]);
-      L[1] = fmaf(D[35], m, L[1]);
-      L[2] = fmaf(D[38], m, L[2]);
-      L[3] = fmaf(D[39], m, L[3]);
-      L[4] = fmaf(D[50], m, L[4]);
-      L[5] = fmaf(D[53], m, L[5]);
-      L[6] = fmaf(D[54], m, L[6]);
-      L[7] = fmaf(D[56], m, L[7]);
-      L[8] = fmaf(D[57], m, L[8]);
-    }
-    { const float m = __ldg(Mr + 21) * rp;
-      L[0] = fmaf(D[25], m, L[0]);
-      L[1] = fmaf(D[37], m, L[1]);
-      L[2] = fmaf(D[40], m, L[2]);
-      L[3] = fmaf(D[41], m, L[3]);
-      L[4] = fmaf(D[52], m, L[4]);
-      L[5] = fmaf(D[55], m, L[5]);
-      L[6] = fmaf(D[56], m, L[6]);
-      L[7] = fmaf(D[58], m, L[7]);
-      L[8] = fmaf(D[59], m, L[8]);
-    }
-    { const float m = __ldg(Mr + 22) * rp;
-      L[0] = fmaf(D[26], m, L[0]);
-      L[1] = fmaf(D[38], m, L[1]);
-      L[2] = fmaf(D[41], m, L[2]);
-      L[3] = fmaf(D[42], m, L[3]);
-      L[4] = fmaf(D[53], m, L[4]);
-      L[5] = fmaf(D[56], m, L[5]);
-      L[6] = fmaf(D[57], m, L[6]);
-      L[7] = fmaf(D[59], m, L[7]);
-      L[8] = fmaf(D[60], m, L[8]);
-    }
-    { const float m = __ldg(Mr + 23) * rp;
-      L[0] = fmaf(D[28], m, L[0]);
-      L[1] = fmaf(D[40], m, L[1]);
-      L[2] = fmaf(D[43], m, L[2]);
-      L[3] = fmaf(D[44], m, L[3]);
-      L[4] = fmaf(D[55], m, L[4]);
-      L[5] = fmaf(D[58], m, L[5]);
-      L[6] = fmaf(D[59], m, L[6]);
-      L[7] = fmaf(D[61], m, L[7]);
-      L[8] = fmaf(D[62], m, L[8]);
-    }
-    { const float m = __ldg(Mr + 24) * rp;
-      L[0] = fmaf(D[29], m, L[0]);
-      L[1] = fmaf(D[41], m, L[1]);
-      L[2] = fmaf(D[44], m, L[2]);
-      L[3] = fmaf(D[45], m, L[3]);
-      L[4] = fmaf(D[56], m, L[4]);
-      L[5] = fmaf(D[59], m, L[5]);
-      L[6] = fmaf(D[60], m, L[6]);
-      L[7] = fmaf(D[62], m, L[7]);
-      L[8] = fmaf(D[63], m, L[8]);
+    { const T m = __ldg(Mr + 8) * rp;
+      L[0] = m2l_fma(D[8], m, L[0]);
+      L[1] = m2l_fma(D[14], m, L[1]);
+      L[2] = m2l_fma(D[17], m, L[2]);
+      L[3] = m2l_fma(D[18], m, L[3]);
+      L[4] = m2l_fma(D[23], m, L[4]);
+      L[5] = m2l_fma(D[26], m, L[5]);
+      L[6] = m2l_fma(D[27], m, L[6]);
+      L[7] = m2l_fma(D[29], m, L[7]);
+      L[8] = m2l_fma(D[30], m, L[8]);
+      L[9] = m2l_fma(D[35], m, L[9]);
+      L[10] = m2l_fma(D[38], m, L[10]);
+      L[11] = m2l_fma(D[39], m, L[11]);
+      L[12] = m2l_fma(D[41], m, L[12]);
+      L[13] = m2l_fma(D[42], m, L[13]);
+      L[14] = m2l_fma(D[44], m, L[14]);
+      L[15] = m2l_fma(D[45], m, L[15]);
+      L[16] = m2l_fma(D[50], m, L[16]);
+      L[17] = m2l_fma(D[53], m, L[17]);
+      L[18] = m2l_fma(D[54], m, L[18]);
+      L[19] = m2l_fma(D[56], m, L[19]);
+      L[20] = m2l_fma(D[57], m, L[20]);
+      L[21] = m2l_fma(D[59], m, L[21]);
+      L[22] = m2l_fma(D[60], m, L[22]);
+      L[23] = m2l_fma(D[62], m, L[23]);
+      L[24] = m2l_fma(D[63], m, L[24]);
     }
     rp *= rho;
-    { const float m = -__ldg(Mr + 25) * rp;
-      L[0] = fmaf(D[31], m, L[0]);
-      L[1] = fmaf(D[46], m, L[1]);
-      L[2] = fmaf(D[47], m, L[2]);
-      L[3] = fmaf(D[48], m, L[3]);
+    { const T m = -__ldg(Mr + 9) * rp;
+      L[0] = m2l_fma(D[10], m, L[0]);
+      L[1] = m2l_fma(D[19], m, L[1]);
+      L[2] = m2l_fma(D[20], m, L[2]);
+      L[3] = m2l_fma(D[21], m, L[3]);
+      L[4] = m2l_fma(D[31], m, L[4]);
+      L[5] = m2l_fma(D[32], m, L[5]);
+      L[6] = m2l_fma(D[33], m, L[6]);
+      L[7] = m2l_fma(D[34], m, L[7]);
+      L[8] = m2l_fma(D[35], m, L[8]);
+      L[9] = m2l_fma(D[46], m, L[9]);
+      L[10] = m2l_fma(D[47], m, L[10]);
+      L[11] = m2l_fma(D[48], m, L[11]);
+      L[12] = m2l_fma(D[49], m, L[12]);
+      L[13] = m2l_fma(D[50], m, L[13]);
+      L[14] = m2l_fma(D[52], m, L[14]);
+      L[15] = m2l_fma(D[53], m, L[15]);
     }
-    { const float m = -__ldg(Mr + 26) * rp;
-      L[0] = fmaf(D[32], m, L[0]);
-      L[1] = fmaf(D[47], m, L[1]);
-      L[2] = fmaf(D[49], m, L[2]);
-      L[3] = fmaf(D[50], m, L[3]);
+    { const T m = -__ldg(Mr + 10) * rp;
+      L[0] = m2l_fma(D[11], m, L[0]);
+      L[1] = m2l_fma(D[20], m, L[1]);
+      L[2] = m2l_fma(D[22], m, L[2]);
+      L[3] = m2l_fma(D[23], m, L[3]);
+      L[4] = m2l_fma(D[32], m, L[4]);
+      L[5] = m2l_fma(D[34], m, L[5]);
+      L[6] = m2l_fma(D[35], m, L[6]);
+      L[7] = m2l_fma(D[37], m, L[7]);
+      L[8] = m2l_fma(D[38], m, L[8]);
+      L[9] = m2l_fma(D[47], m, L[9]);
+      L[10] = m2l_fma(D[49], m, L[10]);
+      L[11] = m2l_fma(D[50], m, L[11]);
+      L[12] = m2l_fma(D[52], m, L[12]);
+      L[13] = m2l_fma(D[53], m, L[13]);
+      L[14] = m2l_fma(D[55], m, L[14]);
+      L[15] = m2l_fma(D[56], m, L[15]);
     }
-    { const float m = -__ldg(Mr + 27) * rp;
-      L[0] = fmaf(D[33], m, L[0]);
-      L[1] = fmaf(D[48], m, L[1]);
-      L[2] = fmaf(D[50], m, L[2]);
-      L[3] = fmaf(D[51], m, L[3]);
+    { const T m = -__ldg(Mr + 11) * rp;
+      L[0] = m2l_fma(D[12], m, L[0]);
+      L[1] = m2l_fma(D[21], m, L[1]);
+      L[2] = m2l_fma(D[23], m, L[2]);
+      L[3] = m2l_fma(D[24], m, L[3]);
+      L[4] = m2l_fma(D[33], m, L[4]);
+      L[5] = m2l_fma(D[35], m, L[5]);
+      L[6] = m2l_fma(D[36], m, L[6]);
+      L[7] = m2l_fma(D[38], m, L[7]);
+      L[8] = m2l_fma(D[39], m, L[8]);
+      L[9] = m2l_fma(D[48], m, L[9]);
+      L[10] = m2l_fma(D[50], m, L[10]);
+      L[11] = m2l_fma(D[51], m, L[11]);
+      L[12] = m2l_fma(D[53], m, L[12]);
+      L[13] = m2l_fma(D[54], m, L[13]);
+      L[14] = m2l_fma(D[56], m, L[14]);
+      L[15] = m2l_fma(D[57], m, L[15]);
     }
-    { const float m = -__ldg(Mr + 28) * rp;
-      L[0] = fmaf(D[34], m, L[0]);
-      L[1] = fmaf(D[49], m, L[1]);
-      L[2] = fmaf(D[52], m, L[2]);
-      L[3] = fmaf(D[53], m, L[3]);
+    { const T m = -__ldg(Mr + 12) * rp;
+      L[0] = m2l_fma(D[13], m, L[0]);
+      L[1] = m2l_fma(D[22], m, L[1]);
+      L[2] = m2l_fma(D[25], m, L[2]);
+      L[3] = m2l_fma(D[26], m, L[3]);
+      L[4] = m2l_fma(D[34], m, L[4]);
+      L[5] = m2l_fma(D[37], m, L[5]);
+      L[6] = m2l_fma(D[38], m, L[6]);
+      L[7] = m2l_fma(D[40], m, L[7]);
+      L[8] = m2l_fma(D[41], m, L[8]);
+      L[9] = m2l_fma(D[49], m, L[9]);
+      L[10] = m2l_fma(D[52], m, L[10]);
+      L[11] = m2l_fma(D[53], m, L[11]);
+      L[12] = m2l_fma(D[55], m, L[12]);
+      L[13] = m2l_fma(D[56], m, L[13]);
+      L[14] = m2l_fma(D[58], m, L[14]);
+      L[15] = m2l_fma(D[59], m, L[15]);
     }
-    { const float m = -__ldg(Mr + 29) * rp;
-      L[0] = fmaf(D[35], m, L[0]);
-      L[1] = fmaf(D[50], m, L[1]);
-      L[2] = fmaf(D[53], m, L[2]);
-      L[3] = fmaf(D[54], m, L[3]);
+    { const T m = -__ldg(Mr + 13) * rp;
+      L[0] = m2l_fma(D[14], m, L[0]);
+      L[1] = m2l_fma(D[23], m, L[1]);
+      L[2] = m2l_fma(D[26], m, L[2]);
+      L[3] = m2l_fma(D[27], m, L[3]);
+      L[4] = m2l_fma(D[35], m, L[4]);
+      L[5] = m2l_fma(D[38], m, L[5]);
+      L[6] = m2l_fma(D[39], m, L[6]);
+      L[7] = m2l_fma(D[41], m, L[7]);
+      L[8] = m2l_fma(D[42], m, L[8]);
+      L[9] = m2l_fma(D[50], m, L[9]);
+      L[10] = m2l_fma(D[53], m, L[10]);
+      L[11] = m2l_fma(D[54], m, L[11]);
+      L[12] = m2l_fma(D[56], m, L[12]);
+      L[13] = m2l_fma(D[57], m, L[13]);
+      L[14] = m2l_fma(D[59], m, L[14]);
+      L[15] = m2l_fma(D[60], m, L[15]);
     }
-    { const float m = -__ldg(Mr + 30) * rp;
-      L[0] = fmaf(D[37], m, L[0]);
-      L[1] = fmaf(D[52], m, L[1]);
-      L[2] = fmaf(D[55], m, L[2]);
-      L[3] = fmaf(D[56], m, L[3]);
+    { const T m = -__ldg(Mr + 14) * rp;
+      L[0] = m2l_fma(D[16], m, L[0]);
+      L[1] = m2l_fma(D[25], m, L[1]);
+      L[2] = m2l_fma(D[28], m, L[2]);
+      L[3] = m2l_fma(D[29], m, L[3]);
+      L[4] = m2l_fma(D[37], m, L[4]);
+      L[5] = m2l_fma(D[40], m, L[5]);
+      L[6] = m2l_fma(D[41], m, L[6]);
+      L[7] = m2l_fma(D[43], m, L[7]);
+      L[8] = m2l_fma(D[44], m, L[8]);
+      L[9] = m2l_fma(D[52], m, L[9]);
+      L[10] = m2l_fma(D[55], m, L[10]);
+      L[11] = m2l_fma(D[56], m, L[11]);
+      L[12] = m2l_fma(D[58], m, L[12]);
+      L[13] = m2l_fma(D[59], m, L[13]);
+      L[14] = m2l_fma(D[61], m, L[14]);
+      L[15] = m2l_fma(D[62], m, L[15]);
     }
-    { const float m = -__ldg(Mr + 31) * rp;
-      L[0] = fmaf(D[38], m, L[0]);
-      L[1] = fmaf(D[53], m, L[1]);
-      L[2] = fmaf(D[56], m, L[2]);
-      L[3] = fmaf(D[57], m, L[3]);
-    }
-    { const float m = -__ldg(Mr + 32) * rp;
-      L[0] = fmaf(D[40], m, L[0]);
-      L[1] = fmaf(D[55], m, L[1]);
-      L[2] = fmaf(D[58], m, L[2]);
-      L[3] = fmaf(D[59], m, L[3]);
-    }
-    { const float m = -__ldg(Mr + 33) * rp;
-      L[0] = fmaf(D[41], m, L[0]);
-      L[1] = fmaf(D[56], m, L[1]);
-      L[2] = fmaf(D[59], m, L[2]);
-      L[3] = fmaf(D[60], m, L[3]);
-    }
-    { const float m = -__ldg(Mr + 34) * rp;
-      L[0] = fmaf(D[43], m, L[0]);
-      L[1] = fmaf(D[58], m, L[1]);
-      L[2] = fmaf(D[61], m, L[2]);
-      L[3] = fmaf(D[62], m, L[3]);
-    }
-    { const float m = -__ldg(Mr + 35) * rp;
-      L[0] = fmaf(D[44], m, L[0]);
-      L[1] = fmaf(D[59], m, L[1]);
-      L[2] = fmaf(D[62], m, L[2]);
-      L[3] = fmaf(D[63], m, L[3]);
+    { const T m = -__ldg(Mr + 15) * rp;
+      L[0] = m2l_fma(D[17], m, L[0]);
+      L[1] = m2l_fma(D[26], m, L[1]);
+      L[2] = m2l_fma(D[29], m, L[2]);
+      L[3] = m2l_fma(D[30], m, L[3]);
+      L[4] = m2l_fma(D[38], m, L[4]);
+      L[5] = m2l_fma(D[41], m, L[5]);
+      L[6] = m2l_fma(D[42], m, L[6]);
+      L[7] = m2l_fma(D[44], m, L[7]);
+      L[8] = m2l_fma(D[45], m, L[8]);
+      L[9] = m2l_fma(D[53], m, L[9]);
+      L[10] = m2l_fma(D[56], m, L[10]);
+      L[11] = m2l_fma(D[57], m, L[11]);
+      L[12] = m2l_fma(D[59], m, L[12]);
+      L[13] = m2l_fma(D[60], m, L[13]);
+      L[14] = m2l_fma(D[62], m, L[14]);
+      L[15] = m2l_fma(D[63], m, L[15]);
     }
     rp *= rho;
-    { const float m = __ldg(Mr + 36) * rp;
-      L[0] = fmaf(D[46], m, L[0]);
+    { const T m = __ldg(Mr + 16) * rp;
+      L[0] = m2l_fma(D[19], m, L[0]);
+      L[1] = m2l_fma(D[31], m, L[1]);
+      L[2] = m2l_fma(D[32], m, L[2]);
+      L[3] = m2l_fma(D[33], m, L[3]);
+      L[4] = m2l_fma(D[46], m, L[4]);
+      L[5] = m2l_fma(D[47], m, L[5]);
+      L[6] = m2l_fma(D[48], m, L[6]);
+      L[7] = m2l_fma(D[49], m, L[7]);
+      L[8] = m2l_fma(D[50], m, L[8]);
     }
-    { const float m = __ldg(Mr + 37) * rp;
-      L[0] = fmaf(D[47], m, L[0]);
+    { const T m = __ldg(Mr + 17) * rp;
+      L[0] = m2l_fma(D[20], m, L[0]);
+      L[1] = m2l_fma(D[32], m, L[1]);
+      L[2] = m2l_fma(D[34], m, L[2]);
+      L[3] = m2l_fma(D[35], m, L[3]);
+      L[4] = m2l_fma(D[47], m, L[4]);
+      L[5] = m2l_fma(D[49], m, L[5]);
+      L[6] = m2l_fma(D[50], m, L[6]);
+      L[7] = m2l_fma(D[52], m, L[7]);
+      L[8] = m2l_fma(D[53], m, L[8]);
     }
-    { const float m = __ldg(Mr + 38) * rp;
-      L[0] = fmaf(D[48], m, L[0]);
+    { const T m = __ldg(Mr + 18) * rp;
+      L[0] = m2l_fma(D[21], m, L[0]);
+      L[1] = m2l_fma(D[33], m, L[1]);
+      L[2] = m2l_fma(D[35], m, L[2]);
+      L[3] = m2l_fma(D[36], m, L[3]);
+      L[4] = m2l_fma(D[48], m, L[4]);
+      L[5] = m2l_fma(D[50], m, L[5]);
+      L[6] = m2l_fma(D[51], m, L[6]);
+      L[7] = m2l_fma(D[53], m, L[7]);
+      L[8] = m2l_fma(D[54], m, L[8]);
     }
-    { const float m = __ldg(Mr + 39) * rp;
-      L[0] = fmaf(D[49], m, L[0]);
+    { const T m = __ldg(Mr + 19) * rp;
+      L[0] = m2l_fma(D[22], m, L[0]);
+      L[1] = m2l_fma(D[34], m, L[1]);
+      L[2] = m2l_fma(D[37], m, L[2]);
+      L[3] = m2l_fma(D[38], m, L[3]);
+      L[4] = m2l_fma(D[49], m, L[4]);
+      L[5] = m2l_fma(D[52], m, L[5]);
+      L[6] = m2l_fma(D[53], m, L[6]);
+      L[7] = m2l_fma(D[55], m, L[7]);
+      L[8] = m2l_fma(D[56], m, L[8]);
     }
-    { const float m = __ldg(Mr + 40) * rp;
-      L[0] = fmaf(D[50], m, L[0]);
+    { const T m = __ldg(Mr + 20) * rp;
+      L[0] = m2l_fma(D[23], m, L[0]);
+      L[1] = m2l_fma(D[35], m, L[1]);
+      L[2] = m2l_fma(D[38], m, L[2]);
+      L[3] = m2l_fma(D[39], m, L[3]);
+      L[4] = m2l_fma(D[50], m, L[4]);
+      L[5] = m2l_fma(D[53], m, L[5]);
+      L[6] = m2l_fma(D[54], m, L[6]);
+      L[7] = m2l_fma(D[56], m, L[7]);
+      L[8] = m2l_fma(D[57], m, L[8]);
     }
-    { const float m = __ldg(Mr + 41) * rp;
-      L[0] = fmaf(D[52], m, L[0]);
+    { const T m = __ldg(Mr + 21) * rp;
+      L[0] = m2l_fma(D[25], m, L[0]);
+      L[1] = m2l_fma(D[37], m, L[1]);
+      L[2] = m2l_fma(D[40], m, L[2]);
+      L[3] = m2l_fma(D[41], m, L[3]);
+      L[4] = m2l_fma(D[52], m, L[4]);
+      L[5] = m2l_fma(D[55], m, L[5]);
+      L[6] = m2l_fma(D[56], m, L[6]);
+      L[7] = m2l_fma(D[58], m, L[7]);
+      L[8] = m2l_fma(D[59], m, L[8]);
     }
-    { const float m = __ldg(Mr + 42) * rp;
-      L[0] = fmaf(D[53], m, L[0]);
+    { const T m = __ldg(Mr + 22) * rp;
+      L[0] = m2l_fma(D[26], m, L[0]);
+      L[1] = m2l_fma(D[38], m, L[1]);
+      L[2] = m2l_fma(D[41], m, L[2]);
+      L[3] = m2l_fma(D[42], m, L[3]);
+      L[4] = m2l_fma(D[53], m, L[4]);
+      L[5] = m2l_fma(D[56], m, L[5]);
+      L[6] = m2l_fma(D[57], m, L[6]);
+      L[7] = m2l_fma(D[59], m, L[7]);
+      L[8] = m2l_fma(D[60], m, L[8]);
     }
-    { const float m = __ldg(Mr + 43) * rp;
-      L[0] = fmaf(D[55], m, L[0]);
+    { const T m = __ldg(Mr + 23) * rp;
+      L[0] = m2l_fma(D[28], m, L[0]);
+      L[1] = m2l_fma(D[40], m, L[1]);
+      L[2] = m2l_fma(D[43], m, L[2]);
+      L[3] = m2l_fma(D[44], m, L[3]);
+      L[4] = m2l_fma(D[55], m, L[4]);
+      L[5] = m2l_fma(D[58], m, L[5]);
+      L[6] = m2l_fma(D[59], m, L[6]);
+      L[7] = m2l_fma(D[61], m, L[7]);
+      L[8] = m2l_fma(D[62], m, L[8]);
     }
-    { const float m = __ldg(Mr + 44) * rp;
-      L[0] = fmaf(D[56], m, L[0]);
+    { const T m = __ldg(Mr + 24) * rp;
+      L[0] = m2l_fma(D[29], m, L[0]);
+      L[1] = m2l_fma(D[41], m, L[1]);
+      L[2] = m2l_fma(D[44], m, L[2]);
+      L[3] = m2l_fma(D[45], m, L[3]);
+      L[4] = m2l_fma(D[56], m, L[4]);
+      L[5] = m2l_fma(D[59], m, L[5]);
+      L[6] = m2l_fma(D[60], m, L[6]);
+      L[7] = m2l_fma(D[62], m, L[7]);
+      L[8] = m2l_fma(D[63], m, L[8]);
     }
-    { const float m = __ldg(Mr + 45) * rp;
-      L[0] = fmaf(D[58], m, L[0]);
+    rp *= rho;
+    { const T m = -__ldg(Mr + 25) * rp;
+      L[0] = m2l_fma(D[31], m, L[0]);
+      L[1] = m2l_fma(D[46], m, L[1]);
+      L[2] = m2l_fma(D[47], m, L[2]);
+      L[3] = m2l_fma(D[48], m, L[3]);
     }
-    { const float m = __ldg(Mr + 46) * rp;
-      L[0] = fmaf(D[59], m, L[0]);
+    { const T m = -__ldg(Mr + 26) * rp;
+      L[0] = m2l_fma(D[32], m, L[0]);
+      L[1] = m2l_fma(D[47], m, L[1]);
+      L[2] = m2l_fma(D[49], m, L[2]);
+      L[3] = m2l_fma(D[50], m, L[3]);
     }
-    { const float m = __ldg(Mr + 47) * rp;
-      L[0] = fmaf(D[61], m, L[0]);
+    { const T m = -__ldg(Mr + 27) * rp;
+      L[0] = m2l_fma(D[33], m, L[0]);
+      L[1] = m2l_fma(D[48], m, L[1]);
+      L[2] = m2l_fma(D[50], m, L[2]);
+      L[3] = m2l_fma(D[51], m, L[3]);
     }
-    { const float m = __ldg(Mr + 48) * rp;
-      L[0] = fmaf(D[62], m, L[0]);
+    { const T m = -__ldg(Mr + 28) * rp;
+      L[0] = m2l_fma(D[34], m, L[0]);
+      L[1] = m2l_fma(D[49], m, L[1]);
+      L[2] = m2l_fma(D[52], m, L[2]);
+      L[3] = m2l_fma(D[53], m, L[3]);
+    }
+    { const T m = -__ldg(Mr + 29) * rp;
+      L[0] = m2l_fma(D[35], m, L[0]);
+      L[1] = m2l_fma(D[50], m, L[1]);
+      L[2] = m2l_fma(D[53], m, L[2]);
+      L[3] = m2l_fma(D[54], m, L[3]);
+    }
+    { const T m = -__ldg(Mr + 30) * rp;
+      L[0] = m2l_fma(D[37], m, L[0]);
+      L[1] = m2l_fma(D[52], m, L[1]);
+      L[2] = m2l_fma(D[55], m, L[2]);
+      L[3] = m2l_fma(D[56], m, L[3]);
+    }
+    { const T m = -__ldg(Mr + 31) * rp;
+      L[0] = m2l_fma(D[38], m, L[0]);
+      L[1] = m2l_fma(D[53], m, L[1]);
+      L[2] = m2l_fma(D[56], m, L[2]);
+      L[3] = m2l_fma(D[57], m, L[3]);
+    }
+    { const T m = -__ldg(Mr + 32) * rp;
+      L[0] = m2l_fma(D[40], m, L[0]);
+      L[1] = m2l_fma(D[55], m, L[1]);
+      L[2] = m2l_fma(D[58], m, L[2]);
+      L[3] = m2l_fma(D[59], m, L[3]);
+    }
+    { const T m = -__ldg(Mr + 33) * rp;
+      L[0] = m2l_fma(D[41], m, L[0]);
+      L[1] = m2l_fma(D[56], m, L[1]);
+      L[2] = m2l_fma(D[59], m, L[2]);
+      L[3] = m2l_fma(D[60], m, L[3]);
+    }
+    { const T m = -__ldg(Mr + 34) * rp;
+      L[0] = m2l_fma(D[43], m, L[0]);
+      L[1] = m2l_fma(D[58], m, L[1]);
+      L[2] = m2l_fma(D[61], m, L[2]);
+      L[3] = m2l_fma(D[62], m, L[3]);
+    }
+    { const T m = -__ldg(Mr + 35) * rp;
+      L[0] = m2l_fma(D[44], m, L[0]);
+      L[1] = m2l_fma(D[59], m, L[1]);
+      L[2] = m2l_fma(D[62], m, L[2]);
+      L[3] = m2l_fma(D[63], m, L[3]);
+    }
+    rp *= rho;
+    { const T m = __ldg(Mr + 36) * rp;
+      L[0] = m2l_fma(D[46], m, L[0]);
+    }
+    { const T m = __ldg(Mr + 37) * rp;
+      L[0] = m2l_fma(D[47], m, L[0]);
+    }
+    { const T m = __ldg(Mr + 38) * rp;
+      L[0] = m2l_fma(D[48], m, L[0]);
+    }
+    { const T m = __ldg(Mr + 39) * rp;
+      L[0] = m2l_fma(D[49], m, L[0]);
+    }
+    { const T m = __ldg(Mr + 40) * rp;
+      L[0] = m2l_fma(D[50], m, L[0]);
+    }
+    { const T m = __ldg(Mr + 41) * rp;
+      L[0] = m2l_fma(D[52], m, L[0]);
+    }
+    { const T m = __ldg(Mr + 42) * rp;
+      L[0] = m2l_fma(D[53], m, L[0]);
+    }
+    { const T m = __ldg(Mr + 43) * rp;
+      L[0] = m2l_fma(D[55], m, L[0]);
+    }
+    { const T m = __ldg(Mr + 44) * rp;
+      L[0] = m2l_fma(D[56], m, L[0]);
+    }
+    { const T m = __ldg(Mr + 45) * rp;
+      L[0] = m2l_fma(D[58], m, L[0]);
+    }
+    { const T m = __ldg(Mr + 46) * rp;
+      L[0] = m2l_fma(D[59], m, L[0]);
+    }
+    { const T m = __ldg(Mr + 47) * rp;
+      L[0] = m2l_fma(D[61], m, L[0]);
+    }
+    { const T m = __ldg(Mr + 48) * rp;
+      L[0] = m2l_fma(D[62], m, L[0]);
     }
 }
 
-__device__ __forceinline__ void m2l_side_b_h_6(const float (&D)[64], const float *__restrict__ Mr, float (&L)[49])
+template <class T> __device__ __forceinline__ void m2l_side_b_h_6(const T (&D)[64], const T *__restrict__ Mr, T (&L)[49])
 {
-    { const float m = __ldg(Mr + 0);
+    { const T m = __ldg(Mr + 0);
       L[0] = D[0] * m;
       L[1] = -D[1] * m;
       L[2] = -D[2] * m;
@@ -15255,592 +15254,592 @@ __device__ __forceinline__ void m2l_side_b_h_6(const float (&D)[64], const float
       L[47] = D[61] * m;
       L[48] = D[62] * m;
     }
-    { const float m = __ldg(Mr + 1);
-      L[0] = fmaf(D[1], m, L[0]);
-      L[1] = fmaf(-D[4], m, L[1]);
-      L[2] = fmaf(-D[5], m, L[2]);
-      L[3] = fmaf(-D[6], m, L[3]);
-      L[4] = fmaf(D[10], m, L[4]);
-      L[5] = fmaf(D[11], m, L[5]);
-      L[6] = fmaf(D[12], m, L[6]);
-      L[7] = fmaf(D[13], m, L[7]);
-      L[8] = fmaf(D[14], m, L[8]);
-      L[9] = fmaf(-D[19], m, L[9]);
-      L[10] = fmaf(-D[20], m, L[10]);
-      L[11] = fmaf(-D[21], m, L[11]);
-      L[12] = fmaf(-D[22], m, L[12]);
-      L[13] = fmaf(-D[23], m, L[13]);
-      L[14] = fmaf(-D[25], m, L[14]);
-      L[15] = fmaf(-D[26], m, L[15]);
-      L[16] = fmaf(D[31], m, L[16]);
-      L[17] = fmaf(D[32], m, L[17]);
-      L[18] = fmaf(D[33], m, L[18]);
-      L[19] = fmaf(D[34], m, L[19]);
-      L[20] = fmaf(D[35], m, L[20]);
-      L[21] = fmaf(D[37], m, L[21]);
-      L[22] = fmaf(D[38], m, L[22]);
-      L[23] = fmaf(D[40], m, L[23]);
-      L[24] = fmaf(D[41], m, L[24]);
-      L[25] = fmaf(-D[46], m, L[25]);
-      L[26] = fmaf(-D[47], m, L[26]);
-      L[27] = fmaf(-D[48], m, L[27]);
-      L[28] = fmaf(-D[49], m, L[28]);
-      L[29] = fmaf(-D[50], m, L[29]);
-      L[30] = fmaf(-D[52], m, L[30]);
-      L[31] = fmaf(-D[53], m, L[31]);
-      L[32] = fmaf(-D[55], m, L[32]);
-      L[33] = fmaf(-D[56], m, L[33]);
-      L[34] = fmaf(-D[58], m, L[34]);
-      L[35] = fmaf(-D[59], m, L[35]);
+    { const T m = __ldg(Mr + 1);
+      L[0] = m2l_fma(D[1], m, L[0]);
+      L[1] = m2l_fma(-D[4], m, L[1]);
+      L[2] = m2l_fma(-D[5], m, L[2]);
+      L[3] = m2l_fma(-D[6], m, L[3]);
+      L[4] = m2l_fma(D[10], m, L[4]);
+      L[5] = m2l_fma(D[11], m, L[5]);
+      L[6] = m2l_fma(D[12], m, L[6]);
+      L[7] = m2l_fma(D[13], m, L[7]);
+      L[8] = m2l_fma(D[14], m, L[8]);
+      L[9] = m2l_fma(-D[19], m, L[9]);
+      L[10] = m2l_fma(-D[20], m, L[10]);
+      L[11] = m2l_fma(-D[21], m, L[11]);
+      L[12] = m2l_fma(-D[22], m, L[12]);
+      L[13] = m2l_fma(-D[23], m, L[13]);
+      L[14] = m2l_fma(-D[25], m, L[14]);
+      L[15] = m2l_fma(-D[26], m, L[15]);
+      L[16] = m2l_fma(D[31], m, L[16]);
+      L[17] = m2l_fma(D[32], m, L[17]);
+      L[18] = m2l_fma(D[33], m, L[18]);
+      L[19] = m2l_fma(D[34], m, L[19]);
+      L[20] = m2l_fma(D[35], m, L[20]);
+      L[21] = m2l_fma(D[37], m, L[21]);
+      L[22] = m2l_fma(D[38], m, L[22]);
+      L[23] = m2l_fma(D[40], m, L[23]);
+      L[24] = m2l_fma(D[41], m, L[24]);
+      L[25] = m2l_fma(-D[46], m, L[25]);
+      L[26] = m2l_fma(-D[47], m, L[26]);
+      L[27] = m2l_fma(-D[48], m, L[27]);
+      L[28] = m2l_fma(-D[49], m, L[28]);
+      L[29] = m2l_fma(-D[50], m, L[29]);
+      L[30] = m2l_fma(-D[52], m, L[30]);
+      L[31] = m2l_fma(-D[53], m, L[31]);
+      L[32] = m2l_fma(-D[55], m, L[32]);
+      L[33] = m2l_fma(-D[56], m, L[33]);
+      L[34] = m2l_fma(-D[58], m, L[34]);
+      L[35] = m2l_fma(-D[59], m, L[35]);
     }
-    { const float m = __ldg(Mr + 2);
-      L[0] = fmaf(D[2], m, L[0]);
-      L[1] = fmaf(-D[5], m, L[1]);
-      L[2] = fmaf(-D[7], m, L[2]);
-      L[3] = fmaf(-D[8], m, L[3]);
-      L[4] = fmaf(D[11], m, L[4]);
-      L[5] = fmaf(D[13], m, L[5]);
-      L[6] = fmaf(D[14], m, L[6]);
-      L[7] = fmaf(D[16], m, L[7]);
-      L[8] = fmaf(D[17], m, L[8]);
-      L[9] = fmaf(-D[20], m, L[9]);
-      L[10] = fmaf(-D[22], m, L[10]);
-      L[11] = fmaf(-D[23], m, L[11]);
-      L[12] = fmaf(-D[25], m, L[12]);
-      L[13] = fmaf(-D[26], m, L[13]);
-      L[14] = fmaf(-D[28], m, L[14]);
-      L[15] = fmaf(-D[29], m, L[15]);
-      L[16] = fmaf(D[32], m, L[16]);
-      L[17] = fmaf(D[34], m, L[17]);
-      L[18] = fmaf(D[35], m, L[18]);
-      L[19] = fmaf(D[37], m, L[19]);
-      L[20] = fmaf(D[38], m, L[20]);
-      L[21] = fmaf(D[40], m, L[21]);
-      L[22] = fmaf(D[41], m, L[22]);
-      L[23] = fmaf(D[43], m, L[23]);
-      L[24] = fmaf(D[44], m, L[24]);
-      L[25] = fmaf(-D[47], m, L[25]);
-      L[26] = fmaf(-D[49], m, L[26]);
-      L[27] = fmaf(-D[50], m, L[27]);
-      L[28] = fmaf(-D[52], m, L[28]);
-      L[29] = fmaf(-D[53], m, L[29]);
-      L[30] = fmaf(-D[55], m, L[30]);
-      L[31] = fmaf(-D[56], m, L[31]);
-      L[32] = fmaf(-D[58], m, L[32]);
-      L[33] = fmaf(-D[59], m, L[33]);
-      L[34] = fmaf(-D[61], m, L[34]);
-      L[35] = fmaf(-D[62], m, L[35]);
+    { const T m = __ldg(Mr + 2);
+      L[0] = m2l_fma(D[2], m, L[0]);
+      L[1] = m2l_fma(-D[5], m, L[1]);
+      L[2] = m2l_fma(-D[7], m, L[2]);
+      L[3] = m2l_fma(-D[8], m, L[3]);
+      L[4] = m2l_fma(D[11], m, L[4]);
+      L[5] = m2l_fma(D[13], m, L[5]);
+      L[6] = m2l_fma(D[14], m, L[6]);
+      L[7] = m2l_fma(D[16], m, L[7]);
+      L[8] = m2l_fma(D[17], m, L[8]);
+      L[9] = m2l_fma(-D[20], m, L[9]);
+      L[10] = m2l_fma(-D[22], m, L[10]);
+      L[11] = m2l_fma(-D[23], m, L[11]);
+      L[12] = m2l_fma(-D[25], m, L[12]);
+      L[13] = m2l_fma(-D[26], m, L[13]);
+      L[14] = m2l_fma(-D[28], m, L[14]);
+      L[15] = m2l_fma(-D[29], m, L[15]);
+      L[16] = m2l_fma(D[32], m, L[16]);
+      L[17] = m2l_fma(D[34], m, L[17]);
+      L[18] = m2l_fma(D[35], m, L[18]);
+      L[19] = m2l_fma(D[37], m, L[19]);
+      L[20] = m2l_fma(D[38], m, L[20]);
+      L[21] = m2l_fma(D[40], m, L[21]);
+      L[22] = m2l_fma(D[41], m, L[22]);
+      L[23] = m2l_fma(D[43], m, L[23]);
+      L[24] = m2l_fma(D[44], m, L[24]);
+      L[25] = m2l_fma(-D[47], m, L[25]);
+      L[26] = m2l_fma(-D[49], m, L[26]);
+      L[27] = m2l_fma(-D[50], m, L[27]);
+      L[28] = m2l_fma(-D[52], m, L[28]);
+      L[29] = m2l_fma(-D[53], m, L[29]);
+      L[30] = m2l_fma(-D[55], m, L[30]);
+      L[31] = m2l_fma(-D[56], m, L[31]);
+      L[32] = m2l_fma(-D[58], m, L[32]);
+      L[33] = m2l_fma(-D[59], m, L[33]);
+      L[34] = m2l_fma(-D[61], m, L[34]);
+      L[35] = m2l_fma(-D[62], m, L[35]);
     }
-    { const float m = __ldg(Mr + 3);
-      L[0] = fmaf(D[3], m, L[0]);
-      L[1] = fmaf(-D[6], m, L[1]);
-      L[2] = fmaf(-D[8], m, L[2]);
-      L[3] = fmaf(-D[9], m, L[3]);
-      L[4] = fmaf(D[12], m, L[4]);
-      L[5] = fmaf(D[14], m, L[5]);
-      L[6] = fmaf(D[15], m, L[6]);
-      L[7] = fmaf(D[17], m, L[7]);
-      L[8] = fmaf(D[18], m, L[8]);
-      L[9] = fmaf(-D[21], m, L[9]);
-      L[10] = fmaf(-D[23], m, L[10]);
-      L[11] = fmaf(-D[24], m, L[11]);
-      L[12] = fmaf(-D[26], m, L[12]);
-      L[13] = fmaf(-D[27], m, L[13]);
-      L[14] = fmaf(-D[29], m, L[14]);
-      L[15] = fmaf(-D[30], m, L[15]);
-      L[16] = fmaf(D[33], m, L[16]);
-      L[17] = fmaf(D[35], m, L[17]);
-      L[18] = fmaf(D[36], m, L[18]);
-      L[19] = fmaf(D[38], m, L[19]);
-      L[20] = fmaf(D[39], m, L[20]);
-      L[21] = fmaf(D[41], m, L[21]);
-      L[22] = fmaf(D[42], m, L[22]);
-      L[23] = fmaf(D[44], m, L[23]);
-      L[24] = fmaf(D[45], m, L[24]);
-      L[25] = fmaf(-D[48], m, L[25]);
-      L[26] = fmaf(-D[50], m, L[26]);
-      L[27] = fmaf(-D[51], m, L[27]);
-      L[28] = fmaf(-D[53], m, L[28]);
-      L[29] = fmaf(-D[54], m, L[29]);
-      L[30] = fmaf(-D[56], m, L[30]);
-      L[31] = fmaf(-D[57], m, L[31]);
-      L[32] = fmaf(-D[59], m, L[32]);
-      L[33] = fmaf(-D[60], m, L[33]);
-      L[34] = fmaf(-D[62], m, L[34]);
-      L[35] = fmaf(-D[63], m, L[35]);
+    { const T m = __ldg(Mr + 3);
+      L[0] = m2l_fma(D[3], m, L[0]);
+      L[1] = m2l_fma(-D[6], m, L[1]);
+      L[2] = m2l_fma(-D[8], m, L[2]);
+      L[3] = m2l_fma(-D[9], m, L[3]);
+      L[4] = m2l_fma(D[12], m, L[4]);
+      L[5] = m2l_fma(D[14], m, L[5]);
+      L[6] = m2l_fma(D[15], m, L[6]);
+      L[7] = m2l_fma(D[17], m, L[7]);
+      L[8] = m2l_fma(D[18], m, L[8]);
+      L[9] = m2l_fma(-D[21], m, L[9]);
+      L[10] = m2l_fma(-D[23], m, L[10]);
+      L[11] = m2l_fma(-D[24], m, L[11]);
+      L[12] = m2l_fma(-D[26], m, L[12]);
+      L[13] = m2l_fma(-D[27], m, L[13]);
+      L[14] = m2l_fma(-D[29], m, L[14]);
+      L[15] = m2l_fma(-D[30], m, L[15]);
+      L[16] = m2l_fma(D[33], m, L[16]);
+      L[17] = m2l_fma(D[35], m, L[17]);
+      L[18] = m2l_fma(D[36], m, L[18]);
+      L[19] = m2l_fma(D[38], m, L[19]);
+      L[20] = m2l_fma(D[39], m, L[20]);
+      L[21] = m2l_fma(D[41], m, L[21]);
+      L[22] = m2l_fma(D[42], m, L[22]);
+      L[23] = m2l_fma(D[44], m, L[23]);
+      L[24] = m2l_fma(D[45], m, L[24]);
+      L[25] = m2l_fma(-D[48], m, L[25]);
+      L[26] = m2l_fma(-D[50], m, L[26]);
+      L[27] = m2l_fma(-D[51], m, L[27]);
+      L[28] = m2l_fma(-D[53], m, L[28]);
+      L[29] = m2l_fma(-D[54], m, L[29]);
+      L[30] = m2l_fma(-D[56], m, L[30]);
+      L[31] = m2l_fma(-D[57], m, L[31]);
+      L[32] = m2l_fma(-D[59], m, L[32]);
+      L[33] = m2l_fma(-D[60], m, L[33]);
+      L[34] = m2l_fma(-D[62], m, L[34]);
+      L[35] = m2l_fma(-D[63], m, L[35]);
     }
-    { const float m = __ldg(Mr + 4);
-      L[0] = fmaf(D[4], m, L[0]);
-      L[1] = fmaf(-D[10], m, L[1]);
-      L[2] = fmaf(-D[11], m, L[2]);
-      L[3] = fmaf(-D[12], m, L[3]);
-      L[4] = fmaf(D[19], m, L[4]);
-      L[5] = fmaf(D[20], m, L[5]);
-      L[6] = fmaf(D[21], m, L[6]);
-      L[7] = fmaf(D[22], m, L[7]);
-      L[8] = fmaf(D[23], m, L[8]);
-      L[9] = fmaf(-D[31], m, L[9]);
-      L[10] = fmaf(-D[32], m, L[10]);
-      L[11] = fmaf(-D[33], m, L[11]);
-      L[12] = fmaf(-D[34], m, L[12]);
-      L[13] = fmaf(-D[35], m, L[13]);
-      L[14] = fmaf(-D[37], m, L[14]);
-      L[15] = fmaf(-D[38], m, L[15]);
-      L[16] = fmaf(D[46], m, L[16]);
-      L[17] = fmaf(D[47], m, L[17]);
-      L[18] = fmaf(D[48], m, L[18]);
-      L[19] = fmaf(D[49], m, L[19]);
-      L[20] = fmaf(D[50], m, L[20]);
-      L[21] = fmaf(D[52], m, L[21]);
-      L[22] = fmaf(D[53], m, L[22]);
-      L[23] = fmaf(D[55], m, L[23]);
-      L[24] = fmaf(D[56], m, L[24]);
+    { const T m = __ldg(Mr + 4);
+      L[0] = m2l_fma(D[4], m, L[0]);
+      L[1] = m2l_fma(-D[10], m, L[1]);
+      L[2] = m2l_fma(-D[11], m, L[2]);
+      L[3] = m2l_fma(-D[12], m, L[3]);
+      L[4] = m2l_fma(D[19], m, L[4]);
+      L[5] = m2l_fma(D[20], m, L[5]);
+      L[6] = m2l_fma(D[21], m, L[6]);
+      L[7] = m2l_fma(D[22], m, L[7]);
+      L[8] = m2l_fma(D[23], m, L[8]);
+      L[9] = m2l_fma(-D[31], m, L[9]);
+      L[10] = m2l_fma(-D[32], m, L[10]);
+      L[11] = m2l_fma(-D[33], m, L[11]);
+      L[12] = m2l_fma(-D[34], m, L[12]);
+      L[13] = m2l_fma(-D[35], m, L[13]);
+      L[14] = m2l_fma(-D[37], m, L[14]);
+      L[15] = m2l_fma(-D[38], m, L[15]);
+      L[16] = m2l_fma(D[46], m, L[16]);
+      L[17] = m2l_fma(D[47], m, L[17]);
+      L[18] = m2l_fma(D[48], m, L[18]);
+      L[19] = m2l_fma(D[49], m, L[19]);
+      L[20] = m2l_fma(D[50], m, L[20]);
+      L[21] = m2l_fma(D[52], m, L[21]);
+      L[22] = m2l_fma(D[53], m, L[22]);
+      L[23] = m2l_fma(D[55], m, L[23]);
+      L[24] = m2l_fma(D[56], m, L[24]);
     }
-    { const float m = __ldg(Mr + 5);
-      L[0] = fmaf(D[5], m, L[0]);
-      L[1] = fmaf(-D[11], m, L[1]);
-      L[2] = fmaf(-D[13], m, L[2]);
-      L[3] = fmaf(-D[14], m, L[3]);
-      L[4] = fmaf(D[20], m, L[4]);
-      L[5] = fmaf(D[22], m, L[5]);
-      L[6] = fmaf(D[23], m, L[6]);
-      L[7] = fmaf(D[25], m, L[7]);
-      L[8] = fmaf(D[26], m, L[8]);
-      L[9] = fmaf(-D[32], m, L[9]);
-      L[10] = fmaf(-D[34], m, L[10]);
-      L[11] = fmaf(-D[35], m, L[11]);
-      L[12] = fmaf(-D[37], m, L[12]);
-      L[13] = fmaf(-D[38], m, L[13]);
-      L[14] = fmaf(-D[40], m, L[14]);
-      L[15] = fmaf(-D[41], m, L[15]);
-      L[16] = fmaf(D[47], m, L[16]);
-      L[17] = fmaf(D[49], m, L[17]);
-      L[18] = fmaf(D[50], m, L[18]);
-      L[19] = fmaf(D[52], m, L[19]);
-      L[20] = fmaf(D[53], m, L[20]);
-      L[21] = fmaf(D[55], m, L[21]);
-      L[22] = fmaf(D[56], m, L[22]);
-      L[23] = fmaf(D[58], m, L[23]);
-      L[24] = fmaf(D[59], m, L[24]);
+    { const T m = __ldg(Mr + 5);
+      L[0] = m2l_fma(D[5], m, L[0]);
+      L[1] = m2l_fma(-D[11], m, L[1]);
+      L[2] = m2l_fma(-D[13], m, L[2]);
+      L[3] = m2l_fma(-D[14], m, L[3]);
+      L[4] = m2l_fma(D[20], m, L[4]);
+      L[5] = m2l_fma(D[22], m, L[5]);
+      L[6] = m2l_fma(D[23], m, L[6]);
+      L[7] = m2l_fma(D[25], m, L[7]);
+      L[8] = m2l_fma(D[26], m, L[8]);
+      L[9] = m2l_fma(-D[32], m, L[9]);
+      L[10] = m2l_fma(-D[34], m, L[10]);
+      L[11] = m2l_fma(-D[35], m, L[11]);
+      L[12] = m2l_fma(-D[37], m, L[12]);
+      L[13] = m2l_fma(-D[38], m, L[13]);
+      L[14] = m2l_fma(-D[40], m, L[14]);
+      L[15] = m2l_fma(-D[41], m, L[15]);
+      L[16] = m2l_fma(D[47], m, L[16]);
+      L[17] = m2l_fma(D[49], m, L[17]);
+      L[18] = m2l_fma(D[50], m, L[18]);
+      L[19] = m2l_fma(D[52], m, L[19]);
+      L[20] = m2l_fma(D[53], m, L[20]);
+      L[21] = m2l_fma(D[55], m, L[21]);
+      L[22] = m2l_fma(D[56], m, L[22]);
+      L[23] = m2l_fma(D[58], m, L[23]);
+      L[24] = m2l_fma(D[59], m, L[24]);
     }
-    { const float m = __ldg(Mr + 6);
-      L[0] = fmaf(D[6], m, L[0]);
-      L[1] = fmaf(-D[12], m, L[1]);
-      L[2] = fmaf(-D[14], m, L[2]);
-      L[3] = fmaf(-D[15], m, L[3]);
-      L[4] = fmaf(D[21], m, L[4]);
-      L[5] = fmaf(D[23], m, L[5]);
-      L[6] = fmaf(D[24], m, L[6]);
-      L[7] = fmaf(D[26], m, L[7]);
-      L[8] = fmaf(D[27], m, L[8]);
-      L[9] = fmaf(-D[33], m, L[9]);
-      L[10] = fmaf(-D[35], m, L[10]);
-      L[11] = fmaf(-D[36], m, L[11]);
-      L[12] = fmaf(-D[38], m, L[12]);
-      L[13] = fmaf(-D[39], m, L[13]);
-      L[14] = fmaf(-D[41], m, L[14]);
-      L[15] = fmaf(-D[42], m, L[15]);
-      L[16] = fmaf(D[48], m, L[16]);
-      L[17] = fmaf(D[50], m, L[17]);
-      L[18] = fmaf(D[51], m, L[18]);
-      L[19] = fmaf(D[53], m, L[19]);
-      L[20] = fmaf(D[54], m, L[20]);
-      L[21] = fmaf(D[56], m, L[21]);
-      L[22] = fmaf(D[57], m, L[22]);
-      L[23] = fmaf(D[59], m, L[23]);
-      L[24] = fmaf(D[60], m, L[24]);
+    { const T m = __ldg(Mr + 6);
+      L[0] = m2l_fma(D[6], m, L[0]);
+      L[1] = m2l_fma(-D[12], m, L[1]);
+      L[2] = m2l_fma(-D[14], m, L[2]);
+      L[3] = m2l_fma(-D[15], m, L[3]);
+      L[4] = m2l_fma(D[21], m, L[4]);
+      L[5] = m2l_fma(D[23], m, L[5]);
+      L[6] = m2l_fma(D[24], m, L[6]);
+      L[7] = m2l_fma(D[26], m, L[7]);
+      L[8] = m2l_fma(D[27], m, L[8]);
+      L[9] = m2l_fma(-D[33], m, L[9]);
+      L[10] = m2l_fma(-D[35], m, L[10]);
+      L[11] = m2l_fma(-D[36], m, L[11]);
+      L[12] = m2l_fma(-D[38], m, L[12]);
+      L[13] = m2l_fma(-D[39], m, L[13]);
+      L[14] = m2l_fma(-D[41], m, L[14]);
+      L[15] = m2l_fma(-D[42], m, L[15]);
+      L[16] = m2l_fma(D[48], m, L[16]);
+      L[17] = m2l_fma(D[50], m, L[17]);
+      L[18] = m2l_fma(D[51], m, L[18]);
+      L[19] = m2l_fma(D[53], m, L[19]);
+      L[20] = m2l_fma(D[54], m, L[20]);
+      L[21] = m2l_fma(D[56], m, L[21]);
+      L[22] = m2l_fma(D[57], m, L[22]);
+      L[23] = m2l_fma(D[59], m, L[23]);
+      L[24] = m2l_fma(D[60], m, L[24]);
     }
-    { const float m = __ldg(Mr + 7);
-      L[0] = fmaf(D[7], m, L[0]);
-      L[1] = fmaf(-D[13], m, L[1]);
-      L[2] = fmaf(-D[16], m, L[2]);
-      L[3] = fmaf(-D[17], m, L[3]);
-      L[4] = fmaf(D[22], m, L[4]);
-      L[5] = fmaf(D[25], m, L[5]);
-      L[6] = fmaf(D[26], m, L[6]);
-      L[7] = fmaf(D[28], m, L[7]);
-      L[8] = fmaf(D[29], m, L[8]);
-      L[9] = fmaf(-D[34], m, L[9]);
-      L[10] = fmaf(-D[37], m, L[10]);
-      L[11] = fmaf(-D[38], m, L[11]);
-      L[12] = fmaf(-D[40], m, L[12]);
-      L[13] = fmaf(-D[41], m, L[13]);
-      L[14] = fmaf(-D[43], m, L[14]);
-      L[15] = fmaf(-D[44], m, L[15]);
-      L[16] = fmaf(D[49], m, L[16]);
-      L[17] = fmaf(D[52], m, L[17]);
-      L[18] = fmaf(D[53], m, L[18]);
-      L[19] = fmaf(D[55], m, L[19]);
-      L[20] = fmaf(D[56], m, L[20]);
-      L[21] = fmaf(D[58], m, L[21]);
-      L[22] = fmaf(D[59], m, L[22]);
-      L[23] = fmaf(D[61], m, L[23]);
-      L[24] = fmaf(D[62], m, L[24]);
+    { const T m = __ldg(Mr + 7);
+      L[0] = m2l_fma(D[7], m, L[0]);
+      L[1] = m2l_fma(-D[13], m, L[1]);
+      L[2] = m2l_fma(-D[16], m, L[2]);
+      L[3] = m2l_fma(-D[17], m, L[3]);
+      L[4] = m2l_fma(D[22], m, L[4]);
+      L[5] = m2l_fma(D[25], m, L[5]);
+      L[6] = m2l_fma(D[26], m, L[6]);
+      L[7] = m2l_fma(D[28], m, L[7]);
+      L[8] = m2l_fma(D[29], m, L[8]);
+      L[9] = m2l_fma(-D[34], m, L[9]);
+      L[10] = m2l_fma(-D[37], m, L[10]);
+      L[11] = m2l_fma(-D[38], m, L[11]);
+      L[12] = m2l_fma(-D[40], m, L[12]);
+      L[13] = m2l_fma(-D[41], m, L[13]);
+      L[14] = m2l_fma(-D[43], m, L[14]);
+      L[15] = m2l_fma(-D[44], m, L[15]);
+      L[16] = m2l_fma(D[49], m, L[16]);
+      L[17] = m2l_fma(D[52], m, L[17]);
+      L[18] = m2l_fma(D[53], m, L[18]);
+      L[19] = m2l_fma(D[55], m, L[19]);
+      L[20] = m2l_fma(D[56], m, L[20]);
+      L[21] = m2l_fma(D[58], m, L[21]);
+      L[22] = m2l_fma(D[59], m, L[22]);
+      L[23] = m2l_fma(D[61], m, L[23]);
+      L[24] = m2l_fma(D[62], m, L[24]);
     }
-    { const float m = __ldg(Mr + 8);
-      L[0] = fmaf(D[8], m, L[0]);
-      L[1] = fmaf(-D[14], m, L[1]);
-      L[2] = fmaf(-D[17], m, L[2]);
-      L[3] = fmaf(-D[18], m, L[3]);
-      L[4] = fmaf(D[23], m, L[4]);
-      L[5] = fmaf(D[26], m, L[5]);
-      L[6] = fmaf(D[27], m, L[6]);
-      L[7] = fmaf(D[29], m, L[7]);
-      L[8] = fmaf(D[30], m, L[8]);
-      L[9] = fmaf(-D[35], m, L[9]);
-      L[10] = fmaf(-D[38], m, L[10]);
-      L[11] = fmaf(-D[39], m, L[11]);
-      L[12] = fmaf(-D[41], m, L[12]);
-      L[13] = fmaf(-D[42], m, L[13]);
-      L[14] = fmaf(-D[44], m, L[14]);
-      L[15] = fmaf(-D[45], m, L[15]);
-      L[16] = fmaf(D[50], m, L[16]);
-      L[17] = fmaf(D[53], m, L[17]);
-      L[18] = fmaf(D[54], m, L[18]);
-      L[19] = fmaf(D[56], m, L[19]);
-      L[20] = fmaf(D[57], m, L[20]);
-      L[21] = fmaf(D[59], m, L[21]);
-      L[22] = fmaf(D[60], m, L[22]);
-      L[23] = fmaf(D[62], m, L[23]);
-      L[24] = fmaf(D[63], m, L[24]);
+    { const T m = __ldg(Mr + 8);
+      L[0] = m2l_fma(D[8], m, L[0]);
+      L[1] = m2l_fma(-D[14], m, L[1]);
+      L[2] = m2l_fma(-D[17], m, L[2]);
+      L[3] = m2l_fma(-D[18], m, L[3]);
+      L[4] = m2l_fma(D[23], m, L[4]);
+      L[5] = m2l_fma(D[26], m, L[5]);
+      L[6] = m2l_fma(D[27], m, L[6]);
+      L[7] = m2l_fma(D[29], m, L[7]);
+      L[8] = m2l_fma(D[30], m, L[8]);
+      L[9] = m2l_fma(-D[35], m, L[9]);
+      L[10] = m2l_fma(-D[38], m, L[10]);
+      L[11] = m2l_fma(-D[39], m, L[11]);
+      L[12] = m2l_fma(-D[41], m, L[12]);
+      L[13] = m2l_fma(-D[42], m, L[13]);
+      L[14] = m2l_fma(-D[44], m, L[14]);
+      L[15] = m2l_fma(-D[45], m, L[15]);
+      L[16] = m2l_fma(D[50], m, L[16]);
+      L[17] = m2l_fma(D[53], m, L[17]);
+      L[18] = m2l_fma(D[54], m, L[18]);
+      L[19] = m2l_fma(D[56], m, L[19]);
+      L[20] = m2l_fma(D[57], m, L[20]);
+      L[21] = m2l_fma(D[59], m, L[21]);
+      L[22] = m2l_fma(D[60], m, L[22]);
+      L[23] = m2l_fma(D[62], m, L[23]);
+      L[24] = m2l_fma(D[63], m, L[24]);
     }
-    { const float m = __ldg(Mr + 9);
-      L[0] = fmaf(D[10], m, L[0]);
-      L[1] = fmaf(-D[19], m, L[1]);
-      L[2] = fmaf(-D[20], m, L[2]);
-      L[3] = fmaf(-D[21], m, L[3]);
-      L[4] = fmaf(D[31], m, L[4]);
-      L[5] = fmaf(D[32], m, L[5]);
-      L[6] = fmaf(D[33], m, L[6]);
-      L[7] = fmaf(D[34], m, L[7]);
-      L[8] = fmaf(D[35], m, L[8]);
-      L[9] = fmaf(-D[46], m, L[9]);
-      L[10] = fmaf(-D[47], m, L[10]);
-      L[11] = fmaf(-D[48], m, L[11]);
-      L[12] = fmaf(-D[49], m, L[12]);
-      L[13] = fmaf(-D[50], m, L[13]);
-      L[14] = fmaf(-D[52], m, L[14]);
-      L[15] = fmaf(-D[53], m, L[15]);
+    { const T m = __ldg(Mr + 9);
+      L[0] = m2l_fma(D[10], m, L[0]);
+      L[1] = m2l_fma(-D[19], m, L[1]);
+      L[2] = m2l_fma(-D[20], m, L[2]);
+      L[3] = m2l_fma(-D[21], m, L[3]);
+      L[4] = m2l_fma(D[31], m, L[4]);
+      L[5] = m2l_fma(D[32], m, L[5]);
+      L[6] = m2l_fma(D[33], m, L[6]);
+      L[7] = m2l_fma(D[34], m, L[7]);
+      L[8] = m2l_fma(D[35], m, L[8]);
+      L[9] = m2l_fma(-D[46], m, L[9]);
+      L[10] = m2l_fma(-D[47], m, L[10]);
+      L[11] = m2l_fma(-D[48], m, L[11]);
+      L[12] = m2l_fma(-D[49], m, L[12]);
+      L[13] = m2l_fma(-D[50], m, L[13]);
+      L[14] = m2l_fma(-D[52], m, L[14]);
+      L[15] = m2l_fma(-D[53], m, L[15]);
     }
-    { const float m = __ldg(Mr + 10);
-      L[0] = fmaf(D[11], m, L[0]);
-      L[1] = fmaf(-D[20], m, L[1]);
-      L[2] = fmaf(-D[22], m, L[2]);
-      L[3] = fmaf(-D[23], m, L[3]);
-      L[4] = fmaf(D[32], m, L[4]);
-      L[5] = fmaf(D[34], m, L[5]);
-      L[6] = fmaf(D[35], m, L[6]);
-      L[7] = fmaf(D[37], m, L[7]);
-      L[8] = fmaf(D[38], m, L[8]);
-      L[9] = fmaf(-D[47], m, L[9]);
-      L[10] = fmaf(-D[49], m, L[10]);
-      L[11] = fmaf(-D[50], m, L[11]);
-      L[12] = fmaf(-D[52], m, L[12]);
-      L[13] = fmaf(-D[53], m, L[13]);
-      L[14] = fmaf(-D[55], m, L[14]);
-      L[15] = fmaf(-D[56], m, L[15]);
+    { const T m = __ldg(Mr + 10);
+      L[0] = m2l_fma(D[11], m, L[0]);
+      L[1] = m2l_fma(-D[20], m, L[1]);
+      L[2] = m2l_fma(-D[22], m, L[2]);
+      L[3] = m2l_fma(-D[23], m, L[3]);
+      L[4] = m2l_fma(D[32], m, L[4]);
+      L[5] = m2l_fma(D[34], m, L[5]);
+      L[6] = m2l_fma(D[35], m, L[6]);
+      L[7] = m2l_fma(D[37], m, L[7]);
+      L[8] = m2l_fma(D[38], m, L[8]);
+      L[9] = m2l_fma(-D[47], m, L[9]);
+      L[10] = m2l_fma(-D[49], m, L[10]);
+      L[11] = m2l_fma(-D[50], m, L[11]);
+      L[12] = m2l_fma(-D[52], m, L[12]);
+      L[13] = m2l_fma(-D[53], m, L[13]);
+      L[14] = m2l_fma(-D[55], m, L[14]);
+      L[15] = m2l_fma(-D[56], m, L[15]);
     }
-    { const float m = __ldg(Mr + 11);
-      L[0] = fmaf(D[12], m, L[0]);
-      L[1] = fmaf(-D[21], m, L[1]);
-      L[2] = fmaf(-D[23], m, L[2]);
-      L[3] = fmaf(-D[24], m, L[3]);
-      L[4] = fmaf(D[33], m, L[4]);
-      L[5] = fmaf(D[35], m, L[5]);
-      L[6] = fmaf(D[36], m, L[6]);
-      L[7] = fmaf(D[38], m, L[7]);
-      L[8] = fmaf(D[39], m, L[8]);
-      L[9] = fmaf(-D[48], m, L[9]);
-      L[10] = fmaf(-D[50], m, L[10]);
-      L[11] = fmaf(-D[51], m, L[11]);
-      L[12] = fmaf(-D[53], m, L[12]);
-      L[13] = fmaf(-D[54], m, L[13]);
-      L[14] = fmaf(-D[56], m, L[14]);
-      L[15] = fmaf(-D[57], m, L[15]);
+    { const T m = __ldg(Mr + 11);
+      L[0] = m2l_fma(D[12], m, L[0]);
+      L[1] = m2l_fma(-D[21], m, L[1]);
+      L[2] = m2l_fma(-D[23], m, L[2]);
+      L[3] = m2l_fma(-D[24], m, L[3]);
+      L[4] = m2l_fma(D[33], m, L[4]);
+      L[5] = m2l_fma(D[35], m, L[5]);
+      L[6] = m2l_fma(D[36], m, L[6]);
+      L[7] = m2l_fma(D[38], m, L[7]);
+      L[8] = m2l_fma(D[39], m, L[8]);
+      L[9] = m2l_fma(-D[48], m, L[9]);
+      L[10] = m2l_fma(-D[50], m, L[10]);
+      L[11] = m2l_fma(-D[51], m, L[11]);
+      L[12] = m2l_fma(-D[53], m, L[12]);
+      L[13] = m2l_fma(-D[54], m, L[13]);
+      L[14] = m2l_fma(-D[56], m, L[14]);
+      L[15] = m2l_fma(-D[57], m, L[15]);
     }
-    { const float m = __ldg(Mr + 12);
-      L[0] = fmaf(D[13], m, L[0]);
-      L[1] = fmaf(-D[22], m, L[1]);
-      L[2] = fmaf(-D[25], m, L[2]);
-      L[3] = fmaf(-D[26], m, L[3]);
-      L[4] = fmaf(D[34], m, L[4]);
-      L[5] = fmaf(D[37], m, L[5]);
-      L[6] = fmaf(D[38], m, L[6]);
-      L[7] = fmaf(D[40], m, L[7]);
-      L[8] = fmaf(D[41], m, L[8]);
-      L[9] = fmaf(-D[49], m, L[9]);
-      L[10] = fmaf(-D[52], m, L[10]);
-      L[11] = fmaf(-D[53], m, L[11]);
-      L[12] = fmaf(-D[55], m, L[12]);
-      L[13] = fmaf(-D[56], m, L[13]);
-      L[14] = fmaf(-D[58], m, L[14]);
-      L[15] = fmaf(-D[59], m, L[15]);
+    { const T m = __ldg(Mr + 12);
+      L[0] = m2l_fma(D[13], m, L[0]);
+      L[1] = m2l_fma(-D[22], m, L[1]);
+      L[2] = m2l_fma(-D[25], m, L[2]);
+      L[3] = m2l_fma(-D[26], m, L[3]);
+      L[4] = m2l_fma(D[34], m, L[4]);
+      L[5] = m2l_fma(D[37], m, L[5]);
+      L[6] = m2l_fma(D[38], m, L[6]);
+      L[7] = m2l_fma(D[40], m, L[7]);
+      L[8] = m2l_fma(D[41], m, L[8]);
+      L[9] = m2l_fma(-D[49], m, L[9]);
+      L[10] = m2l_fma(-D[52], m, L[10]);
+      L[11] = m2l_fma(-D[53], m, L[11]);
+      L[12] = m2l_fma(-D[55], m, L[12]);
+      L[13] = m2l_fma(-D[56], m, L[13]);
+      L[14] = m2l_fma(-D[58], m, L[14]);
+      L[15] = m2l_fma(-D[59], m, L[15]);
     }
-    { const float m = __ldg(Mr + 13);
-      L[0] = fmaf(D[14], m, L[0]);
-      L[1] = fmaf(-D[23], m, L[1]);
-      L[2] = fmaf(-D[26], m, L[2]);
-      L[3] = fmaf(-D[27], m, L[3]);
-      L[4] = fmaf(D[35], m, L[4]);
-      L[5] = fmaf(D[38], m, L[5]);
-      L[6] = fmaf(D[39], m, L[6]);
-      L[7] = fmaf(D[41], m, L[7]);
-      L[8] = fmaf(D[42], m, L[8]);
-      L[9] = fmaf(-D[50], m, L[9]);
-      L[10] = fmaf(-D[53], m, L[10]);
-      L[11] = fmaf(-D[54], m, L[11]);
-      L[12] = fmaf(-D[56], m, L[12]);
-      L[13] = fmaf(-D[57], m, L[13]);
-      L[14] = fmaf(-D[59], m, L[14]);
-      L[15] = fmaf(-D[60], m, L[15]);
+    { const T m = __ldg(Mr + 13);
+      L[0] = m2l_fma(D[14], m, L[0]);
+      L[1] = m2l_fma(-D[23], m, L[1]);
+      L[2] = m2l_fma(-D[26], m, L[2]);
+      L[3] = m2l_fma(-D[27], m, L[3]);
+      L[4] = m2l_fma(D[35], m, L[4]);
+      L[5] = m2l_fma(D[38], m, L[5]);
+      L[6] = m2l_fma(D[39], m, L[6]);
+      L[7] = m2l_fma(D[41], m, L[7]);
+      L[8] = m2l_fma(D[42], m, L[8]);
+      L[9] = m2l_fma(-D[50], m, L[9]);
+      L[10] = m2l_fma(-D[53], m, L[10]);
+      L[11] = m2l_fma(-D[54], m, L[11]);
+      L[12] = m2l_fma(-D[56], m, L[12]);
+      L[13] = m2l_fma(-D[57], m, L[13]);
+      L[14] = m2l_fma(-D[59], m, L[14]);
+      L[15] = m2l_fma(-D[60], m, L[15]);
     }
-    { const float m = __ldg(Mr + 14);
-      L[0] = fmaf(D[16], m, L[0]);
-      L[1] = fmaf(-D[25], m, L[1]);
-      L[2] = fmaf(-D[28], m, L[2]);
-      L[3] = fmaf(-D[29], m, L[3]);
-      L[4] = fmaf(D[37], m, L[4]);
-      L[5] = fmaf(D[40], m, L[5]);
-      L[6] = fmaf(D[41], m, L[6]);
-      L[7] = fmaf(D[43], m, L[7]);
-      L[8] = fmaf(D[44], m, L[8]);
-      L[9] = fmaf(-D[52], m, L[9]);
-      L[10] = fmaf(-D[55], m, L[10]);
-      L[11] = fmaf(-D[56], m, L[11]);
-      L[12] = fmaf(-D[58], m, L[12]);
-      L[13] = fmaf(-D[59], m, L[13]);
-      L[14] = fmaf(-D[61], m, L[14]);
-      L[15] = fmaf(-D[62], m, L[15]);
+    { const T m = __ldg(Mr + 14);
+      L[0] = m2l_fma(D[16], m, L[0]);
+      L[1] = m2l_fma(-D[25], m, L[1]);
+      L[2] = m2l_fma(-D[28], m, L[2]);
+      L[3] = m2l_fma(-D[29], m, L[3]);
+      L[4] = m2l_fma(D[37], m, L[4]);
+      L[5] = m2l_fma(D[40], m, L[5]);
+      L[6] = m2l_fma(D[41], m, L[6]);
+      L[7] = m2l_fma(D[43], m, L[7]);
+      L[8] = m2l_fma(D[44], m, L[8]);
+      L[9] = m2l_fma(-D[52], m, L[9]);
+      L[10] = m2l_fma(-D[55], m, L[10]);
+      L[11] = m2l_fma(-D[56], m, L[11]);
+      L[12] = m2l_fma(-D[58], m, L[12]);
+      L[13] = m2l_fma(-D[59], m, L[13]);
+      L[14] = m2l_fma(-D[61], m, L[14]);
+      L[15] = m2l_fma(-D[62], m, L[15]);
     }
-    { const float m = __ldg(Mr + 15);
-      L[0] = fmaf(D[17], m, L[0]);
-      L[1] = fmaf(-D[26], m, L[1]);
-      L[2] = fmaf(-D[29], m, L[2]);
-      L[3] = fmaf(-D[30], m, L[3]);
-      L[4] = fmaf(D[38], m, L[4]);
-      L[5] = fmaf(D[41], m, L[5]);
-      L[6] = fmaf(D[42], m, L[6]);
-      L[7] = fmaf(D[44], m, L[7]);
-      L[8] = fmaf(D[45], m, L[8]);
-      L[9] = fmaf(-D[53], m, L[9]);
-      L[10] = fmaf(-D[56], m, L[10]);
-      L[11] = fmaf(-D[57], m, L[11]);
-      L[12] = fmaf(-D[59], m, L[12]);
-      L[13] = fmaf(-D[60], m, L[13]);
-      L[14] = fmaf(-D[62], m, L[14]);
-      L[15] = fmaf(-D[63], m, L[15]);
+    { const T m = __ldg(Mr + 15);
+      L[0] = m2l_fma(D[17], m, L[0]);
+      L[1] = m2l_fma(-D[26], m, L[1]);
+      L[2] = m2l_fma(-D[29], m, L[2]);
+      L[3] = m2l_fma(-D[30], m, L[3]);
+      L[4] = m2l_fma(D[38], m, L[4]);
+      L[5] = m2l_fma(D[41], m, L[5]);
+      L[6] = m2l_fma(D[42], m, L[6]);
+      L[7] = m2l_fma(D[44], m, L[7]);
+      L[8] = m2l_fma(D[45], m, L[8]);
+      L[9] = m2l_fma(-D[53], m, L[9]);
+      L[10] = m2l_fma(-D[56], m, L[10]);
+      L[11] = m2l_fma(-D[57], m, L[11]);
+      L[12] = m2l_fma(-D[59], m, L[12]);
+      L[13] = m2l_fma(-D[60], m, L[13]);
+      L[14] = m2l_fma(-D[62], m, L[14]);
+      L[15] = m2l_fma(-D[63], m, L[15]);
     }
-    { const float m = __ldg(Mr + 16);
-      L[0] = fmaf(D[19], m, L[0]);
-      L[1] = fmaf(-D[31], m, L[1]);
-      L[2] = fmaf(-D[32], m, L[2]);
-      L[3] = fmaf(-D[33], m, L[3]);
-      L[4] = fmaf(D[46], m, L[4]);
-      L[5] = fmaf(D[47], m, L[5]);
-      L[6] = fmaf(D[48], m, L[6]);
-      L[7] = fmaf(D[49], m, L[7]);
-      L[8] = fmaf(D[50], m, L[8]);
+    { const T m = __ldg(Mr + 16);
+      L[0] = m2l_fma(D[19], m, L[0]);
+      L[1] = m2l_fma(-D[31], m, L[1]);
+      L[2] = m2l_fma(-D[32], m, L[2]);
+      L[3] = m2l_fma(-D[33], m, L[3]);
+      L[4] = m2l_fma(D[46], m, L[4]);
+      L[5] = m2l_fma(D[47], m, L[5]);
+      L[6] = m2l_fma(D[48], m, L[6]);
+      L[7] = m2l_fma(D[49], m, L[7]);
+      L[8] = m2l_fma(D[50], m, L[8]);
     }
-    { const float m = __ldg(Mr + 17);
-      L[0] = fmaf(D[20], m, L[0]);
-      L[1] = fmaf(-D[32], m, L[1]);
-      L[2] = fmaf(-D[34], m, L[2]);
-      L[3] = fmaf(-D[35], m, L[3]);
-      L[4] = fmaf(D[47], m, L[4]);
-      L[5] = fmaf(D[49], m, L[5]);
-      L[6] = fmaf(D[50], m, L[6]);
-      L[7] = fmaf(D[52], m, L[7]);
-      L[8] = fmaf(D[53], m, L[8]);
+    { const T m = __ldg(Mr + 17);
+      L[0] = m2l_fma(D[20], m, L[0]);
+      L[1] = m2l_fma(-D[32], m, L[1]);
+      L[2] = m2l_fma(-D[34], m, L[2]);
+      L[3] = m2l_fma(-D[35], m, L[3]);
+      L[4] = m2l_fma(D[47], m, L[4]);
+      L[5] = m2l_fma(D[49], m, L[5]);
+      L[6] = m2l_fma(D[50], m, L[6]);
+      L[7] = m2l_fma(D[52], m, L[7]);
+      L[8] = m2l_fma(D[53], m, L[8]);
     }
-    { const float m = __ldg(Mr + 18);
-      L[0] = fmaf(D[21], m, L[0]);
-      L[1] = fmaf(-D[33], m, L[1]);
-      L[2] = fmaf(-D[35], m, L[2]);
-      L[3] = fmaf(-D[36], m, L[3]);
-      L[4] = fmaf(D[48], m, L[4]);
-      L[5] = fmaf(D[50], m, L[5]);
-      L[6] = fmaf(D[51], m, L[6]);
-      L[7] = fmaf(D[53], m, L[7]);
-      L[8] = fmaf(D[54], m, L[8]);
+    { const T m = __ldg(Mr + 18);
+      L[0] = m2l_fma(D[21], m, L[0]);
+      L[1] = m2l_fma(-D[33], m, L[1]);
+      L[2] = m2l_fma(-D[35], m, L[2]);
+      L[3] = m2l_fma(-D[36], m, L[3]);
+      L[4] = m2l_fma(D[48], m, L[4]);
+      L[5] = m2l_fma(D[50], m, L[5]);
+      L[6] = m2l_fma(D[51], m, L[6]);
+      L[7] = m2l_fma(D[53], m, L[7]);
+      L[8] = m2l_fma(D[54], m, L[8]);
     }
-    { const float m = __ldg(Mr + 19);
-      L[0] = fmaf(D[22], m, L[0]);
-      L[1] = fmaf(-D[34], m, L[1]);
-      L[2] = fmaf(-D[37], m, L[2]);
-      L[3] = fmaf(-D[38], m, L[3]);
-      L[4] = fmaf(D[49], m, L[4]);
-      L[5] = fmaf(D[52], m, L[5]);
-      L[6] = fmaf(D[53], m, L[6]);
-      L[7] = fmaf(D[55], m, L[7]);
-      L[8] = fmaf(D[56], m, L[8]);
+    { const T m = __ldg(Mr + 19);
+      L[0] = m2l_fma(D[22], m, L[0]);
+      L[1] = m2l_fma(-D[34], m, L[1]);
+      L[2] = m2l_fma(-D[37], m, L[2]);
+      L[3] = m2l_fma(-D[38], m, L[3]);
+      L[4] = m2l_fma(D[49], m, L[4]);
+      L[5] = m2l_fma(D[52], m, L[5]);
+      L[6] = m2l_fma(D[53], m, L[6]);
+      L[7] = m2l_fma(D[55], m, L[7]);
+      L[8] = m2l_fma(D[56], m, L[8]);
     }
-    { const float m = __ldg(Mr + 20);
-      L[0] = fmaf(D[23], m, L[0]);
-      L[1] = fmaf(-D[35], m, L[1]);
-      L[2] = fmaf(-D[38], m, L[2]);
-      L[3] = fmaf(-D[39], m, L[3]);
-      L[4] = fmaf(D[50], m, L[4]);
-      L[5] = fmaf(D[53], m, L[5]);
-      L[6] = fmaf(D[54], m, L[6]);
-      L[7] = fmaf(D[56], m, L[7]);
-      L[8] = fmaf(D[57], m, L[8]);
+    { const T m = __ldg(Mr + 20);
+      L[0] = m2l_fma(D[23], m, L[0]);
+      L[1] = m2l_fma(-D[35], m, L[1]);
+      L[2] = m2l_fma(-D[38], m, L[2]);
+      L[3] = m2l_fma(-D[39], m, L[3]);
+      L[4] = m2l_fma(D[50], m, L[4]);
+      L[5] = m2l_fma(D[53], m, L[5]);
+      L[6] = m2l_fma(D[54], m, L[6]);
+      L[7] = m2l_fma(D[56], m, L[7]);
+      L[8] = m2l_fma(D[57], m, L[8]);
     }
-    { const float m = __ldg(Mr + 21);
-      L[0] = fmaf(D[25], m, L[0]);
-      L[1] = fmaf(-D[37], m, L[1]);
-      L[2] = fmaf(-D[40], m, L[2]);
-      L[3] = fmaf(-D[41], m, L[3]);
-      L[4] = fmaf(D[52], m, L[4]);
-      L[5] = fmaf(D[55], m, L[5]);
-      L[6] = fmaf(D[56], m, L[6]);
-      L[7] = fmaf(D[58], m, L[7]);
-      L[8] = fmaf(D[59], m, L[8]);
+    { const T m = __ldg(Mr + 21);
+      L[0] = m2l_fma(D[25], m, L[0]);
+      L[1] = m2l_fma(-D[37], m, L[1]);
+      L[2] = m2l_fma(-D[40], m, L[2]);
+      L[3] = m2l_fma(-D[41], m, L[3]);
+      L[4] = m2l_fma(D[52], m, L[4]);
+      L[5] = m2l_fma(D[55], m, L[5]);
+      L[6] = m2l_fma(D[56], m, L[6]);
+      L[7] = m2l_fma(D[58], m, L[7]);
+      L[8] = m2l_fma(D[59], m, L[8]);
     }
-    { const float m = __ldg(Mr + 22);
-      L[0] = fmaf(D[26], m, L[0]);
-      L[1] = fmaf(-D[38], m, L[1]);
-      L[2] = fmaf(-D[41], m, L[2]);
-      L[3] = fmaf(-D[42], m, L[3]);
-      L[4] = fmaf(D[53], m, L[4]);
-      L[5] = fmaf(D[56], m, L[5]);
-      L[6] = fmaf(D[57], m, L[6]);
-      L[7] = fmaf(D[59], m, L[7]);
-      L[8] = fmaf(D[60], m, L[8]);
+    { const T m = __ldg(Mr + 22);
+      L[0] = m2l_fma(D[26], m, L[0]);
+      L[1] = m2l_fma(-D[38], m, L[1]);
+      L[2] = m2l_fma(-D[41], m, L[2]);
+      L[3] = m2l_fma(-D[42], m, L[3]);
+      L[4] = m2l_fma(D[53], m, L[4]);
+      L[5] = m2l_fma(D[56], m, L[5]);
+      L[6] = m2l_fma(D[57], m, L[6]);
+      L[7] = m2l_fma(D[59], m, L[7]);
+      L[8] = m2l_fma(D[60], m, L[8]);
     }
-    { const float m = __ldg(Mr + 23);
-      L[0] = fmaf(D[28], m, L[0]);
-      L[1] = fmaf(-D[40], m, L[1]);
-      L[2] = fmaf(-D[43], m, L[2]);
-      L[3] = fmaf(-D[44], m, L[3]);
-      L[4] = fmaf(D[55], m, L[4]);
-      L[5] = fmaf(D[58], m, L[5]);
-      L[6] = fmaf(D[59], m, L[6]);
-      L[7] = fmaf(D[61], m, L[7]);
-      L[8] = fmaf(D[62], m, L[8]);
+    { const T m = __ldg(Mr + 23);
+      L[0] = m2l_fma(D[28], m, L[0]);
+      L[1] = m2l_fma(-D[40], m, L[1]);
+      L[2] = m2l_fma(-D[43], m, L[2]);
+      L[3] = m2l_fma(-D[44], m, L[3]);
+      L[4] = m2l_fma(D[55], m, L[4]);
+      L[5] = m2l_fma(D[58], m, L[5]);
+      L[6] = m2l_fma(D[59], m, L[6]);
+      L[7] = m2l_fma(D[61], m, L[7]);
+      L[8] = m2l_fma(D[62], m, L[8]);
     }
-    { const float m = __ldg(Mr + 24);
-      L[0] = fmaf(D[29], m, L[0]);
-      L[1] = fmaf(-D[41], m, L[1]);
-      L[2] = fmaf(-D[44], m, L[2]);
-      L[3] = fmaf(-D[45], m, L[3]);
-      L[4] = fmaf(D[56], m, L[4]);
-      L[5] = fmaf(D[59], m, L[5]);
-      L[6] = fmaf(D[60], m, L[6]);
-      L[7] = fmaf(D[62], m, L[7]);
-      L[8] = fmaf(D[63], m, L[8]);
+    { const T m = __ldg(Mr + 24);
+      L[0] = m2l_fma(D[29], m, L[0]);
+      L[1] = m2l_fma(-D[41], m, L[1]);
+      L[2] = m2l_fma(-D[44], m, L[2]);
+      L[3] = m2l_fma(-D[45], m, L[3]);
+      L[4] = m2l_fma(D[56], m, L[4]);
+      L[5] = m2l_fma(D[59], m, L[5]);
+      L[6] = m2l_fma(D[60], m, L[6]);
+      L[7] = m2l_fma(D[62], m, L[7]);
+      L[8] = m2l_fma(D[63], m, L[8]);
     }
-    { const float m = __ldg(Mr + 25);
-      L[0] = fmaf(D[31], m, L[0]);
-      L[1] = fmaf(-D[46], m, L[1]);
-      L[2] = fmaf(-D[47], m, L[2]);
-      L[3] = fmaf(-D[48], m, L[3]);
+    { const T m = __ldg(Mr + 25);
+      L[0] = m2l_fma(D[31], m, L[0]);
+      L[1] = m2l_fma(-D[46], m, L[1]);
+      L[2] = m2l_fma(-D[47], m, L[2]);
+      L[3] = m2l_fma(-D[48], m, L[3]);
     }
-    { const float m = __ldg(Mr + 26);
-      L[0] = fmaf(D[32], m, L[0]);
-      L[1] = fmaf(-D[47], m, L[1]);
-      L[2] = fmaf(-D[49], m, L[2]);
-      L[3] = fmaf(-D[50], m, L[3]);
+    { const T m = __ldg(Mr + 26);
+      L[0] = m2l_fma(D[32], m, L[0]);
+      L[1] = m2l_fma(-D[47], m, L[1]);
+      L[2] = m2l_fma(-D[49], m, L[2]);
+      L[3] = m2l_fma(-D[50], m, L[3]);
     }
-    { const float m = __ldg(Mr + 27);
-      L[0] = fmaf(D[33], m, L[0]);
-      L[1] = fmaf(-D[48], m, L[1]);
-      L[2] = fmaf(-D[50], m, L[2]);
-      L[3] = fmaf(-D[51], m, L[3]);
+    { const T m = __ldg(Mr + 27);
+      L[0] = m2l_fma(D[33], m, L[0]);
+      L[1] = m2l_fma(-D[48], m, L[1]);
+      L[2] = m2l_fma(-D[50], m, L[2]);
+      L[3] = m2l_fma(-D[51], m, L[3]);
     }
-    { const float m = __ldg(Mr + 28);
-      L[0] = fmaf(D[34], m, L[0]);
-      L[1] = fmaf(-D[49], m, L[1]);
-      L[2] = fmaf(-D[52], m, L[2]);
-      L[3] = fmaf(-D[53], m, L[3]);
+    { const T m = __ldg(Mr + 28);
+      L[0] = m2l_fma(D[34], m, L[0]);
+      L[1] = m2l_fma(-D[49], m, L[1]);
+      L[2] = m2l_fma(-D[52], m, L[2]);
+      L[3] = m2l_fma(-D[53], m, L[3]);
     }
-    { const float m = __ldg(Mr + 29);
-      L[0] = fmaf(D[35], m, L[0]);
-      L[1] = fmaf(-D[50], m, L[1]);
-      L[2] = fmaf(-D[53], m, L[2]);
-      L[3] = fmaf(-D[54], m, L[3]);
+    { const T m = __ldg(Mr + 29);
+      L[0] = m2l_fma(D[35], m, L[0]);
+      L[1] = m2l_fma(-D[50], m, L[1]);
+      L[2] = m2l_fma(-D[53], m, L[2]);
+      L[3] = m2l_fma(-D[54], m, L[3]);
     }
-    { const float m = __ldg(Mr + 30);
-      L[0] = fmaf(D[37], m, L[0]);
-      L[1] = fmaf(-D[52], m, L[1]);
-      L[2] = fmaf(-D[55], m, L[2]);
-      L[3] = fmaf(-D[56], m, L[3]);
+    { const T m = __ldg(Mr + 30);
+      L[0] = m2l_fma(D[37], m, L[0]);
+      L[1] = m2l_fma(-D[52], m, L[1]);
+      L[2] = m2l_fma(-D[55], m, L[2]);
+      L[3] = m2l_fma(-D[56], m, L[3]);
     }
-    { const float m = __ldg(Mr + 31);
-      L[0] = fmaf(D[38], m, L[0]);
-      L[1] = fmaf(-D[53], m, L[1]);
-      L[2] = fmaf(-D[56], m, L[2]);
-      L[3] = fmaf(-D[57], m, L[3]);
+    { const T m = __ldg(Mr + 31);
+      L[0] = m2l_fma(D[38], m, L[0]);
+      L[1] = m2l_fma(-D[53], m, L[1]);
+      L[2] = m2l_fma(-D[56], m, L[2]);
+      L[3] = m2l_fma(-D[57], m, L[3]);
     }
-    { const float m = __ldg(Mr + 32);
-      L[0] = fmaf(D[40], m, L[0]);
-      L[1] = fmaf(-D[55], m, L[1]);
-      L[2] = fmaf(-D[58], m, L[2]);
-      L[3] = fmaf(-D[59], m, L[3]);
+    { const T m = __ldg(Mr + 32);
+      L[0] = m2l_fma(D[40], m, L[0]);
+      L[1] = m2l_fma(-D[55], m, L[1]);
+      L[2] = m2l_fma(-D[58], m, L[2]);
+      L[3] = m2l_fma(-D[59], m, L[3]);
     }
-    { const float m = __ldg(Mr + 33);
-      L[0] = fmaf(D[41], m, L[0]);
-      L[1] = fmaf(-D[56], m, L[1]);
-      L[2] = fmaf(-D[59], m, L[2]);
-      L[3] = fmaf(-D[60], m, L[3]);
+    { const T m = __ldg(Mr + 33);
+      L[0] = m2l_fma(D[41], m, L[0]);
+      L[1] = m2l_fma(-D[56], m, L[1]);
+      L[2] = m2l_fma(-D[59], m, L[2]);
+      L[3] = m2l_fma(-D[60], m, L[3]);
     }
-    { const float m = __ldg(Mr + 34);
-      L[0] = fmaf(D[43], m, L[0]);
-      L[1] = fmaf(-D[58], m, L[1]);
-      L[2] = fmaf(-D[61], m, L[2]);
-      L[3] = fmaf(-D[62], m, L[3]);
+    { const T m = __ldg(Mr + 34);
+      L[0] = m2l_fma(D[43], m, L[0]);
+      L[1] = m2l_fma(-D[58], m, L[1]);
+      L[2] = m2l_fma(-D[61], m, L[2]);
+      L[3] = m2l_fma(-D[62], m, L[3]);
     }
-    { const float m = __ldg(Mr + 35);
-      L[0] = fmaf(D[44], m, L[0]);
-      L[1] = fmaf(-D[59], m, L[1]);
-      L[2] = fmaf(-D[62], m, L[2]);
-      L[3] = fmaf(-D[63], m, L[3]);
+    { const T m = __ldg(Mr + 35);
+      L[0] = m2l_fma(D[44], m, L[0]);
+      L[1] = m2l_fma(-D[59], m, L[1]);
+      L[2] = m2l_fma(-D[62], m, L[2]);
+      L[3] = m2l_fma(-D[63], m, L[3]);
     }
-    { const float m = __ldg(Mr + 36);
-      L[0] = fmaf(D[46], m, L[0]);
+    { const T m = __ldg(Mr + 36);
+      L[0] = m2l_fma(D[46], m, L[0]);
     }
-    { const float m = __ldg(Mr + 37);
-      L[0] = fmaf(D[47], m, L[0]);
+    { const T m = __ldg(Mr + 37);
+      L[0] = m2l_fma(D[47], m, L[0]);
     }
-    { const float m = __ldg(Mr + 38);
-      L[0] = fmaf(D[48], m, L[0]);
+    { const T m = __ldg(Mr + 38);
+      L[0] = m2l_fma(D[48], m, L[0]);
     }
-    { const float m = __ldg(Mr + 39);
-      L[0] = fmaf(D[49], m, L[0]);
+    { const T m = __ldg(Mr + 39);
+      L[0] = m2l_fma(D[49], m, L[0]);
     }
-    { const float m = __ldg(Mr + 40);
-      L[0] = fmaf(D[50], m, L[0]);
+    { const T m = __ldg(Mr + 40);
+      L[0] = m2l_fma(D[50], m, L[0]);
     }
-    { const float m = __ldg(Mr + 41);
-      L[0] = fmaf(D[52], m, L[0]);
+    { const T m = __ldg(Mr + 41);
+      L[0] = m2l_fma(D[52], m, L[0]);
     }
-    { const float m = __ldg(Mr + 42);
-      L[0] = fmaf(D[53], m, L[0]);
+    { const T m = __ldg(Mr + 42);
+      L[0] = m2l_fma(D[53], m, L[0]);
     }
-    { const float m = __ldg(Mr + 43);
-      L[0] = fmaf(D[55], m, L[0]);
+    { const T m = __ldg(Mr + 43);
+      L[0] = m2l_fma(D[55], m, L[0]);
     }
-    { const float m = __ldg(Mr + 44);
-      L[0] = fmaf(D[56], m, L[0]);
+    { const T m = __ldg(Mr + 44);
+      L[0] = m2l_fma(D[56], m, L[0]);
     }
-    { const float m = __ldg(Mr + 45);
-      L[0] = fmaf(D[58], m, L[0]);
+    { const T m = __ldg(Mr + 45);
+      L[0] = m2l_fma(D[58], m, L[0]);
     }
-    { const float m = __ldg(Mr + 46);
-      L[0] = fmaf(D[59], m, L[0]);
+    { const T m = __ldg(Mr + 46);
+      L[0] = m2l_fma(D[59], m, L[0]);
     }
-    { const float m = __ldg(Mr + 47);
-      L[0] = fmaf(D[61], m, L[0]);
+    { const T m = __ldg(Mr + 47);
+      L[0] = m2l_fma(D[61], m, L[0]);
     }
-    { const float m = __ldg(Mr + 48);
-      L[0] = fmaf(D[62], m, L[0]);
+    { const T m = __ldg(Mr + 48);
+      L[0] = m2l_fma(D[62], m, L[0]);
     }
 }
 
-__device__ __forceinline__ void m2l_side_a_h_forces_6(const float (&D)[64], const float *__restrict__ Mr, float rho, float (&L)[49])
+template <class T> __device__ __forceinline__ void m2l_side_a_h_forces_6(const T (&D)[64], const T *__restrict__ Mr, T rho, T (&L)[49])
 {
-    L[0] = 0.0f;
-    float rp = 1.0f;
-    { const float m = __ldg(Mr + 0) * rp;
+    L[0] = T(0);
+    T rp = T(1);
+    { const T m = __ldg(Mr + 0) * rp;
       L[1] = D[1] * m;
       L[2] = D[2] * m;
       L[3] = D[3] * m;
@@ -15891,1086 +15890,1086 @@ __device__ __forceinline__ void m2l_side_a_h_forces_6(const float (&D)[64], cons
       L[48] = D[62] * m;
     }
     rp *= rho;
-    { const float m = -__ldg(Mr + 1) * rp;
-      L[1] = fmaf(D[4], m, L[1]);
-      L[2] = fmaf(D[5], m, L[2]);
-      L[3] = fmaf(D[6], m, L[3]);
-      L[4] = fmaf(D[10], m, L[4]);
-      L[5] = fmaf(D[11], m, L[5]);
-      L[6] = fmaf(D[12], m, L[6]);
-      L[7] = fmaf(D[13], m, L[7]);
-      L[8] = fmaf(D[14], m, L[8]);
-      L[9] = fmaf(D[19], m, L[9]);
-      L[10] = fmaf(D[20], m, L[10]);
-      L[11] = fmaf(D[21], m, L[11]);
-      L[12] = fmaf(D[22], m, L[12]);
-      L[13] = fmaf(D[23], m, L[13]);
-      L[14] = fmaf(D[25], m, L[14]);
-      L[15] = fmaf(D[26], m, L[15]);
-      L[16] = fmaf(D[31], m, L[16]);
-      L[17] = fmaf(D[32], m, L[17]);
-      L[18] = fmaf(D[33], m, L[18]);
-      L[19] = fmaf(D[34], m, L[19]);
-      L[20] = fmaf(D[35], m, L[20]);
-      L[21] = fmaf(D[37], m, L[21]);
-      L[22] = fmaf(D[38], m, L[22]);
-      L[23] = fmaf(D[40], m, L[23]);
-      L[24] = fmaf(D[41], m, L[24]);
-      L[25] = fmaf(D[46], m, L[25]);
-      L[26] = fmaf(D[47], m, L[26]);
-      L[27] = fmaf(D[48], m, L[27]);
-      L[28] = fmaf(D[49], m, L[28]);
-      L[29] = fmaf(D[50], m, L[29]);
-      L[30] = fmaf(D[52], m, L[30]);
-      L[31] = fmaf(D[53], m, L[31]);
-      L[32] = fmaf(D[55], m, L[32]);
-      L[33] = fmaf(D[56], m, L[33]);
-      L[34] = fmaf(D[58], m, L[34]);
-      L[35] = fmaf(D[59], m, L[35]);
+    { const T m = -__ldg(Mr + 1) * rp;
+      L[1] = m2l_fma(D[4], m, L[1]);
+      L[2] = m2l_fma(D[5], m, L[2]);
+      L[3] = m2l_fma(D[6], m, L[3]);
+      L[4] = m2l_fma(D[10], m, L[4]);
+      L[5] = m2l_fma(D[11], m, L[5]);
+      L[6] = m2l_fma(D[12], m, L[6]);
+      L[7] = m2l_fma(D[13], m, L[7]);
+      L[8] = m2l_fma(D[14], m, L[8]);
+      L[9] = m2l_fma(D[19], m, L[9]);
+      L[10] = m2l_fma(D[20], m, L[10]);
+      L[11] = m2l_fma(D[21], m, L[11]);
+      L[12] = m2l_fma(D[22], m, L[12]);
+      L[13] = m2l_fma(D[23], m, L[13]);
+      L[14] = m2l_fma(D[25], m, L[14]);
+      L[15] = m2l_fma(D[26], m, L[15]);
+      L[16] = m2l_fma(D[31], m, L[16]);
+      L[17] = m2l_fma(D[32], m, L[17]);
+      L[18] = m2l_fma(D[33], m, L[18]);
+      L[19] = m2l_fma(D[34], m, L[19]);
+      L[20] = m2l_fma(D[35], m, L[20]);
+      L[21] = m2l_fma(D[37], m, L[21]);
+      L[22] = m2l_fma(D[38], m, L[22]);
+      L[23] = m2l_fma(D[40], m, L[23]);
+      L[24] = m2l_fma(D[41], m, L[24]);
+      L[25] = m2l_fma(D[46], m, L[25]);
+      L[26] = m2l_fma(D[47], m, L[26]);
+      L[27] = m2l_fma(D[48], m, L[27]);
+      L[28] = m2l_fma(D[49], m, L[28]);
+      L[29] = m2l_fma(D[50], m, L[29]);
+      L[30] = m2l_fma(D[52], m, L[30]);
+      L[31] = m2l_fma(D[53], m, L[31]);
+      L[32] = m2l_fma(D[55], m, L[32]);
+      L[33] = m2l_fma(D[56], m, L[33]);
+      L[34] = m2l_fma(D[58], m, L[34]);
+      L[35] = m2l_fma(D[59], m, L[35]);
     }
-    { const float m = -__ldg(Mr + 2) * rp;
-      L[1] = fmaf(D[5], m, L[1]);
-      L[2] = fmaf(D[7], m, L[2]);
-      L[3] = fmaf(D[8], m, L[3]);
-      L[4] = fmaf(D[11], m, L[4]);
-      L[5] = fmaf(D[13], m, L[5]);
-      L[6] = fmaf(D[14], m, L[6]);
-      L[7] = fmaf(D[16], m, L[7]);
-      L[8] = fmaf(D[17], m, L[8]);
-      L[9] = fmaf(D[20], m, L[9]);
-      L[10] = fmaf(D[22], m, L[10]);
-      L[11] = fmaf(D[23], m, L[11]);
-      L[12] = fmaf(D[25], m, L[12]);
-      L[13] = fmaf(D[26], m, L[13]);
-      L[14] = fmaf(D[28], m, L[14]);
-      L[15] = fmaf(D[29], m, L[15]);
-      L[16] = fmaf(D[32], m, L[16]);
-      L[17] = fmaf(D[34], m, L[17]);
-      L[18] = fmaf(D[35], m, L[18]);
-      L[19] = fmaf(D[37], m, L[19]);
-      L[20] = fmaf(D[38], m, L[20]);
-      L[21] = fmaf(D[40], m, L[21]);
-      L[22] = fmaf(D[41], m, L[22]);
-      L[23] = fmaf(D[43], m, L[23]);
-      L[24] = fmaf(D[44], m, L[24]);
-      L[25] = fmaf(D[47], m, L[25]);
-      L[26] = fmaf(D[49], m, L[26]);
-      L[27] = fmaf(D[50], m, L[27]);
-      L[28] = fmaf(D[52], m, L[28]);
-      L[29] = fmaf(D[53], m, L[29]);
-      L[30] = fmaf(D[55], m, L[30]);
-      L[31] = fmaf(D[56], m, L[31]);
-      L[32] = fmaf(D[58], m, L[32]);
-      L[33] = fmaf(D[59], m, L[33]);
-      L[34] = fmaf(D[61], m, L[34]);
-      L[35] = fmaf(D[62], m, L[35]);
+    { const T m = -__ldg(Mr + 2) * rp;
+      L[1] = m2l_fma(D[5], m, L[1]);
+      L[2] = m2l_fma(D[7], m, L[2]);
+      L[3] = m2l_fma(D[8], m, L[3]);
+      L[4] = m2l_fma(D[11], m, L[4]);
+      L[5] = m2l_fma(D[13], m, L[5]);
+      L[6] = m2l_fma(D[14], m, L[6]);
+      L[7] = m2l_fma(D[16], m, L[7]);
+      L[8] = m2l_fma(D[17], m, L[8]);
+      L[9] = m2l_fma(D[20], m, L[9]);
+      L[10] = m2l_fma(D[22], m, L[10]);
+      L[11] = m2l_fma(D[23], m, L[11]);
+      L[12] = m2l_fma(D[25], m, L[12]);
+      L[13] = m2l_fma(D[26], m, L[13]);
+      L[14] = m2l_fma(D[28], m, L[14]);
+      L[15] = m2l_fma(D[29], m, L[15]);
+      L[16] = m2l_fma(D[32], m, L[16]);
+      L[17] = m2l_fma(D[34], m, L[17]);
+      L[18] = m2l_fma(D[35], m, L[18]);
+      L[19] = m2l_fma(D[37], m, L[19]);
+      L[20] = m2l_fma(D[38], m, L[20]);
+      L[21] = m2l_fma(D[40], m, L[21]);
+      L[22] = m2l_fma(D[41], m, L[22]);
+      L[23] = m2l_fma(D[43], m, L[23]);
+      L[24] = m2l_fma(D[44], m, L[24]);
+      L[25] = m2l_fma(D[47], m, L[25]);
+      L[26] = m2l_fma(D[49], m, L[26]);
+      L[27] = m2l_fma(D[50], m, L[27]);
+      L[28] = m2l_fma(D[52], m, L[28]);
+      L[29] = m2l_fma(D[53], m, L[29]);
+      L[30] = m2l_fma(D[55], m, L[30]);
+      L[31] = m2l_fma(D[56], m, L[31]);
+      L[32] = m2l_fma(D[58], m, L[32]);
+      L[33] = m2l_fma(D[59], m, L[33]);
+      L[34] = m2l_fma(D[61], m, L[34]);
+      L[35] = m2l_fma(D[62], m, L[35]);
     }
-    { const float m = -__ldg(Mr + 3) * rp;
-      L[1] = fmaf(D[6], m, L[1]);
-      L[2] = fmaf(D[8], m, L[2]);
-      L[3] = fmaf(D[9], m, L[3]);
-      L[4] = fmaf(D[12], m, L[4]);
-      L[5] = fmaf(D[14], m, L[5]);
-      L[6] = fmaf(D[15], m, L[6]);
-      L[7] = fmaf(D[17], m, L[7]);
-      L[8] = fmaf(D[18], m, L[8]);
-      L[9] = fmaf(D[21], m, L[9]);
-      L[10] = fmaf(D[23], m, L[10]);
-      L[11] = fmaf(D[24], m, L[11]);
-      L[12] = fmaf(D[26], m, L[12]);
-      L[13] = fmaf(D[27], m, L[13]);
-      L[14] = fmaf(D[29], m, L[14]);
-      L[15] = fmaf(D[30], m, L[15]);
-      L[16] = fmaf(D[33], m, L[16]);
-      L[17] = fmaf(D[35], m, L[17]);
-      L[18] = fmaf(D[36], m, L[18]);
-      L[19] = fmaf(D[38], m, L[19]);
-      L[20] = fmaf(D[39], m, L[20]);
-      L[21] = fmaf(D[41], m, L[21]);
-      L[22] = fmaf(D[42], m, L[22]);
-      L[23] = fmaf(D[44], m, L[23]);
-      L[24] = fmaf(D[45], m, L[24]);
-      L[25] = fmaf(D[48], m, L[25]);
-      L[26] = fmaf(D[50], m, L[26]);
-      L[27] = fmaf(D[51], m, L[27]);
-      L[28] = fmaf(D[53], m, L[28]);
-      L[29] = fmaf(D[54], m, L[29]);
-      L[30] = fmaf(D[56], m, L[30]);
-      L[31] = fmaf(D[57], m, L[31]);
-      L[32] = fmaf(D[59], m, L[32]);
-      L[33] = fmaf(D[60], m, L[33]);
-      L[34] = fmaf(D[62], m, L[34]);
-      L[35] = fmaf(D[63], m, L[35]);
-    }
-    rp *= rho;
-    { const float m = __ldg(Mr + 4) * rp;
-      L[1] = fmaf(D[10], m, L[1]);
-      L[2] = fmaf(D[11], m, L[2]);
-      L[3] = fmaf(D[12], m, L[3]);
-      L[4] = fmaf(D[19], m, L[4]);
-      L[5] = fmaf(D[20], m, L[5]);
-      L[6] = fmaf(D[21], m, L[6]);
-      L[7] = fmaf(D[22], m, L[7]);
-      L[8] = fmaf(D[23], m, L[8]);
-      L[9] = fmaf(D[31], m, L[9]);
-      L[10] = fmaf(D[32], m, L[10]);
-      L[11] = fmaf(D[33], m, L[11]);
-      L[12] = fmaf(D[34], m, L[12]);
-      L[13] = fmaf(D[35], m, L[13]);
-      L[14] = fmaf(D[37], m, L[14]);
-      L[15] = fmaf(D[38], m, L[15]);
-      L[16] = fmaf(D[46], m, L[16]);
-      L[17] = fmaf(D[47], m, L[17]);
-      L[18] = fmaf(D[48], m, L[18]);
-      L[19] = fmaf(D[49], m, L[19]);
-      L[20] = fmaf(D[50], m, L[20]);
-      L[21] = fmaf(D[52], m, L[21]);
-      L[22] = fmaf(D[53], m, L[22]);
-      L[23] = fmaf(D[55], m, L[23]);
-      L[24] = fmaf(D[56], m, L[24]);
-    }
-    { const float m = __ldg(Mr + 5) * rp;
-      L[1] = fmaf(D[11], m, L[1]);
-      L[2] = fmaf(D[13], m, L[2]);
-      L[3] = fmaf(D[14], m, L[3]);
-      L[4] = fmaf(D[20], m, L[4]);
-      L[5] = fmaf(D[22], m, L[5]);
-      L[6] = fmaf(D[23], m, L[6]);
-      L[7] = fmaf(D[25], m, L[7]);
-      L[8] = fmaf(D[26], m, L[8]);
-      L[9] = fmaf(D[32], m, L[9]);
-      L[10] = fmaf(D[34], m, L[10]);
-      L[11] = fmaf(D[35], m, L[11]);
-      L[12] = fmaf(D[37], m, L[12]);
-      L[13] = fmaf(D[38], m, L[13]);
-      L[14] = fmaf(D[40], m, L[14]);
-      L[15] = fmaf(D[41], m, L[15]);
-      L[16] = fmaf(D[47], m, L[16]);
-      L[17] = fmaf(D[49], m, L[17]);
-      L[18] = fmaf(D[50], m, L[18]);
-      L[19] = fmaf(D[52], m, L[19]);
-      L[20] = fmaf(D[53], m, L[20]);
-      L[21] = fmaf(D[55], m, L[21]);
-      L[22] = fmaf(D[56], m, L[22]);
-      L[23] = fmaf(D[58], m, L[23]);
-      L[24] = fmaf(D[59], m, L[24]);
-    }
-    { const float m = __ldg(Mr + 6) * rp;
-      L[1] = fmaf(D[12], m, L[1]);
-      L[2] = fmaf(D[14], m, L[2]);
-      L[3] = fmaf(D[15], m, L[3]);
-      L[4] = fmaf(D[21], m, L[4]);
-      L[5] = fmaf(D[23], m, L[5]);
-      L[6] = fmaf(D[24], m, L[6]);
-      L[7] = fmaf(D[26], m, L[7]);
-      L[8] = fmaf(D[27], m, L[8]);
-      L[9] = fmaf(D[33], m, L[9]);
-      L[10] = fmaf(D[35], m, L[10]);
-      L[11] = fmaf(D[36], m, L[11]);
-      L[12] = fmaf(D[38], m, L[12]);
-      L[13] = fmaf(D[39], m, L[13]);
-      L[14] = fmaf(D[41], m, L[14]);
-      L[15] = fmaf(D[42], m, L[15]);
-      L[16] = fmaf(D[48], m, L[16]);
-      L[17] = fmaf(D[50], m, L[17]);
-      L[18] = fmaf(D[51], m, L[18]);
-      L[19] = fmaf(D[53], m, L[19]);
-      L[20] = fmaf(D[54], m, L[20]);
-      L[21] = fmaf(D[56], m, L[21]);
-      L[22] = fmaf(D[57], m, L[22]);
-      L[23] = fmaf(D[59], m, L[23]);
-      L[24] = fmaf(D[60], m, L[24]);
-    }
-    { const float m = __ldg(Mr + 7) * rp;
-      L[1] = fmaf(D[13], m, L[1]);
-      L[2] = fmaf(D[16], m, L[2]);
-      L[3] = fmaf(D[17], m, L[3]);
-      L[4] = fmaf(D[22], m, L[4]);
-      L[5] = fmaf(D[25], m, L[5]);
-      L[6] = fmaf(D[26], m, L[6]);
-      L[7] = fmaf(D[28], m, L[7]);
-      L[8] = fmaf(D[29], m, L[8]);
-      L[9] = fmaf(D[34], m, L[9]);
-      L[10] = fmaf(D[37], m, L[10]);
-      L[11] = fmaf(D[38], m, L[11]);
-      L[12] = fmaf(D[40], m, L[12]);
-      L[13] = fmaf(D[41], m, L[13]);
-      L[14] = fmaf(D[43], m, L[14]);
-      L[15] = fmaf(D[44], m, L[15]);
-      L[16] = fmaf(D[49], m, L[16]);
-      L[17] = fmaf(D[52], m, L[17]);
-      L[18] = fmaf(D[53], m, L[18]);
-      L[19] = fmaf(D[55], m, L[19]);
-      L[20] = fmaf(D[56], m, L[20]);
-      L[21] = fmaf(D[58], m, L[21]);
-      L[22] = fmaf(D[59], m, L[22]);
-      L[23] = fmaf(D[61], m, L[23]);
-      L[24] = fmaf(D[62], m, L[24]);
-    }
-    { const float m = __ldg(Mr + 8) * rp;
-      L[1] = fmaf(D[14], m, L[1]);
-      L[2] = fmaf(D[17], m, L[2]);
-      L[3] = fmaf(D[18], m, L[3]);
-      L[4] = fmaf(D[23], m, L[4]);
-      L[5] = fmaf(D[26], m, L[5]);
-      L[6] = fmaf(D[27], m, L[6]);
-      L[7] = fmaf(D[29], m, L[7]);
-      L[8] = fmaf(D[30], m, L[8]);
-      L[9] = fmaf(D[35], m, L[9]);
-      L[10] = fmaf(D[38], m, L[10]);
-      L[11] = fmaf(D[39], m, L[11]);
-      L[12] = fmaf(D[41], m, L[12]);
-      L[13] = fmaf(D[42], m, L[13]);
-      L[14] = fmaf(D[44], m, L[14]);
-      L[15] = fmaf(D[45], m, L[15]);
-      L[16] = fmaf(D[50], m, L[16]);
-      L[17] = fmaf(D[53], m, L[17]);
-      L[18] = fmaf(D[54], m, L[18]);
-      L[19] = fmaf(D[56], m, L[19]);
-      L[20] = fmaf(D[57], m, L[20]);
-      L[21] = fmaf(D[59], m, L[21]);
-      L[22] = fmaf(D[60], m, L[22]);
-      L[23] = fmaf(D[62], m, L[23]);
-      L[24] = fmaf(D[63], m, L[24]);
+    { const T m = -__ldg(Mr + 3) * rp;
+      L[1] = m2l_fma(D[6], m, L[1]);
+      L[2] = m2l_fma(D[8], m, L[2]);
+      L[3] = m2l_fma(D[9], m, L[3]);
+      L[4] = m2l_fma(D[12], m, L[4]);
+      L[5] = m2l_fma(D[14], m, L[5]);
+      L[6] = m2l_fma(D[15], m, L[6]);
+      L[7] = m2l_fma(D[17], m, L[7]);
+      L[8] = m2l_fma(D[18], m, L[8]);
+      L[9] = m2l_fma(D[21], m, L[9]);
+      L[10] = m2l_fma(D[23], m, L[10]);
+      L[11] = m2l_fma(D[24], m, L[11]);
+      L[12] = m2l_fma(D[26], m, L[12]);
+      L[13] = m2l_fma(D[27], m, L[13]);
+      L[14] = m2l_fma(D[29], m, L[14]);
+      L[15] = m2l_fma(D[30], m, L[15]);
+      L[16] = m2l_fma(D[33], m, L[16]);
+      L[17] = m2l_fma(D[35], m, L[17]);
+      L[18] = m2l_fma(D[36], m, L[18]);
+      L[19] = m2l_fma(D[38], m, L[19]);
+      L[20] = m2l_fma(D[39], m, L[20]);
+      L[21] = m2l_fma(D[41], m, L[21]);
+      L[22] = m2l_fma(D[42], m, L[22]);
+      L[23] = m2l_fma(D[44], m, L[23]);
+      L[24] = m2l_fma(D[45], m, L[24]);
+      L[25] = m2l_fma(D[48], m, L[25]);
+      L[26] = m2l_fma(D[50], m, L[26]);
+      L[27] = m2l_fma(D[51], m, L[27]);
+      L[28] = m2l_fma(D[53], m, L[28]);
+      L[29] = m2l_fma(D[54], m, L[29]);
+      L[30] = m2l_fma(D[56], m, L[30]);
+      L[31] = m2l_fma(D[57], m, L[31]);
+      L[32] = m2l_fma(D[59], m, L[32]);
+      L[33] = m2l_fma(D[60], m, L[33]);
+      L[34] = m2l_fma(D[62], m, L[34]);
+      L[35] = m2l_fma(D[63], m, L[35]);
     }
     rp *= rho;
-    { const float m = -__ldg(Mr + 9) * rp;
-      L[1] = fmaf(D[19], m, L[1]);
-      L[2] = fmaf(D[20], m, L[2]);
-      L[3] = fmaf(D[21], m, L[3]);
-      L[4] = fmaf(D[31], m, L[4]);
-      L[5] = fmaf(D[32], m, L[5]);
-      L[6] = fmaf(D[33], m, L[6]);
-      L[7] = fmaf(D[34], m, L[7]);
-      L[8] = fmaf(D[35], m, L[8]);
-      L[9] = fmaf(D[46], m, L[9]);
-      L[10] = fmaf(D[47], m, L[10]);
-      L[11] = fmaf(D[48], m, L[11]);
-      L[12] = fmaf(D[49], m, L[12]);
-      L[13] = fmaf(D[50], m, L[13]);
-      L[14] = fmaf(D[52], m, L[14]);
-      L[15] = fmaf(D[53], m, L[15]);
+    { const T m = __ldg(Mr + 4) * rp;
+      L[1] = m2l_fma(D[10], m, L[1]);
+      L[2] = m2l_fma(D[11], m, L[2]);
+      L[3] = m2l_fma(D[12], m, L[3]);
+      L[4] = m2l_fma(D[19], m, L[4]);
+      L[5] = m2l_fma(D[20], m, L[5]);
+      L[6] = m2l_fma(D[21], m, L[6]);
+      L[7] = m2l_fma(D[22], m, L[7]);
+      L[8] = m2l_fma(D[23], m, L[8]);
+      L[9] = m2l_fma(D[31], m, L[9]);
+      L[10] = m2l_fma(D[32], m, L[10]);
+      L[11] = m2l_fma(D[33], m, L[11]);
+      L[12] = m2l_fma(D[34], m, L[12]);
+      L[13] = m2l_fma(D[35], m, L[13]);
+      L[14] = m2l_fma(D[37], m, L[14]);
+      L[15] = m2l_fma(D[38], m, L[15]);
+      L[16] = m2l_fma(D[46], m, L[16]);
+      L[17] = m2l_fma(D[47], m, L[17]);
+      L[18] = m2l_fma(D[48], m, L[18]);
+      L[19] = m2l_fma(D[49], m, L[19]);
+      L[20] = m2l_fma(D[50], m, L[20]);
+      L[21] = m2l_fma(D[52], m, L[21]);
+      L[22] = m2l_fma(D[53], m, L[22]);
+      L[23] = m2l_fma(D[55], m, L[23]);
+      L[24] = m2l_fma(D[56], m, L[24]);
     }
-    { const float m = -__ldg(Mr + 10) * rp;
-      L[1] = fmaf(D[20], m, L[1]);
-      L[2] = fmaf(D[22], m, L[2]);
-      L[3] = fmaf(D[23], m, L[3]);
-      L[4] = fmaf(D[32], m, L[4]);
-      L[5] = fmaf(D[34], m, L[5]);
-      L[6] = fmaf(D[35], m, L[6]);
-      L[7] = fmaf(D[37], m, L[7]);
-      L[8] = fmaf(D[38], m, L[8]);
-      L[9] = fmaf(D[47], m, L[9]);
-      L[10] = fmaf(D[49], m, L[10]);
-      L[11] = fmaf(D[50], m, L[11]);
-      L[12] = fmaf(D[52], m, L[12]);
-      L[13] = fmaf(D[53], m, L[13]);
-      L[14] = fmaf(D[55], m, L[14]);
-      L[15] = fmaf(D[56], m, L[15]);
+    { const T m = __ldg(Mr + 5) * rp;
+      L[1] = m2l_fma(D[11], m, L[1]);
+      L[2] = m2l_fma(D[13], m, L[2]);
+      L[3] = m2l_fma(D[14], m, L[3]);
+      L[4] = m2l_fma(D[20], m, L[4]);
+      L[5] = m2l_fma(D[22], m, L[5]);
+      L[6] = m2l_fma(D[23], m, L[6]);
+      L[7] = m2l_fma(D[25], m, L[7]);
+      L[8] = m2l_fma(D[26], m, L[8]);
+      L[9] = m2l_fma(D[32], m, L[9]);
+      L[10] = m2l_fma(D[34], m, L[10]);
+      L[11] = m2l_fma(D[35], m, L[11]);
+      L[12] = m2l_fma(D[37], m, L[12]);
+      L[13] = m2l_fma(D[38], m, L[13]);
+      L[14] = m2l_fma(D[40], m, L[14]);
+      L[15] = m2l_fma(D[41], m, L[15]);
+      L[16] = m2l_fma(D[47], m, L[16]);
+      L[17] = m2l_fma(D[49], m, L[17]);
+      L[18] = m2l_fma(D[50], m, L[18]);
+      L[19] = m2l_fma(D[52], m, L[19]);
+      L[20] = m2l_fma(D[53], m, L[20]);
+      L[21] = m2l_fma(D[55], m, L[21]);
+      L[22] = m2l_fma(D[56], m, L[22]);
+      L[23] = m2l_fma(D[58], m, L[23]);
+      L[24] = m2l_fma(D[59], m, L[24]);
     }
-    { const float m = -__ldg(Mr + 11) * rp;
-      L[1] = fmaf(D[21], m, L[1]);
-      L[2] = fmaf(D[23], m, L[2]);
-      L[3] = fmaf(D[24], m, L[3]);
-      L[4] = fmaf(D[33], m, L[4]);
-      L[5] = fmaf(D[35], m, L[5]);
-      L[6] = fmaf(D[36], m, L[6]);
-      L[7] = fmaf(D[38], m, L[7]);
-      L[8] = fmaf(D[39], m, L[8]);
-      L[9] = fmaf(D[48], m, L[9]);
-      L[10] = fmaf(D[50], m, L[10]);
-      L[11] = fmaf(D[51], m, L[11]);
-      L[12] = fmaf(D[53], m, L[12]);
-      L[13] = fmaf(D[54], m, L[13]);
-      L[14] = fmaf(D[56], m, L[14]);
-      L[15] = fmaf(D[57], m, L[15]);
+    { const T m = __ldg(Mr + 6) * rp;
+      L[1] = m2l_fma(D[12], m, L[1]);
+      L[2] = m2l_fma(D[14], m, L[2]);
+      L[3] = m2l_fma(D[15], m, L[3]);
+      L[4] = m2l_fma(D[21], m, L[4]);
+      L[5] = m2l_fma(D[23], m, L[5]);
+      L[6] = m2l_fma(D[24], m, L[6]);
+      L[7] = m2l_fma(D[26], m, L[7]);
+      L[8] = m2l_fma(D[27], m, L[8]);
+      L[9] = m2l_fma(D[33], m, L[9]);
+      L[10] = m2l_fma(D[35], m, L[10]);
+      L[11] = m2l_fma(D[36], m, L[11]);
+      L[12] = m2l_fma(D[38], m, L[12]);
+      L[13] = m2l_fma(D[39], m, L[13]);
+      L[14] = m2l_fma(D[41], m, L[14]);
+      L[15] = m2l_fma(D[42], m, L[15]);
+      L[16] = m2l_fma(D[48], m, L[16]);
+      L[17] = m2l_fma(D[50], m, L[17]);
+      L[18] = m2l_fma(D[51], m, L[18]);
+      L[19] = m2l_fma(D[53], m, L[19]);
+      L[20] = m2l_fma(D[54], m, L[20]);
+      L[21] = m2l_fma(D[56], m, L[21]);
+      L[22] = m2l_fma(D[57], m, L[22]);
+      L[23] = m2l_fma(D[59], m, L[23]);
+      L[24] = m2l_fma(D[60], m, L[24]);
     }
-    { const float m = -__ldg(Mr + 12) * rp;
-      L[1] = fmaf(D[22], m, L[1]);
-      L[2] = fmaf(D[25], m, L[2]);
-      L[3] = fmaf(D[26], m, L[3]);
-      L[4] = fmaf(D[34], m, L[4]);
-      L[5] = fmaf(D[37], m, L[5]);
-      L[6] = fmaf(D[38], m, L[6]);
-      L[7] = fmaf(D[40], m, L[7]);
-      L[8] = fmaf(D[41], m, L[8]);
-      L[9] = fmaf(D[49], m, L[9]);
-      L[10] = fmaf(D[52], m, L[10]);
-      L[11] = fmaf(D[53], m, L[11]);
-      L[12] = fmaf(D[55], m, L[12]);
-      L[13] = fmaf(D[56], m, L[13]);
-      L[14] = fmaf(D[58], m, L[14]);
-      L[15] = fmaf(D[59], m, L[15]);
+    { const T m = __ldg(Mr + 7) * rp;
+      L[1] = m2l_fma(D[13], m, L[1]);
+      L[2] = m2l_fma(D[16], m, L[2]);
+      L[3] = m2l_fma(D[17], m, L[3]);
+      L[4] = m2l_fma(D[22], m, L[4]);
+      L[5] = m2l_fma(D[25], m, L[5]);
+      L[6] = m2l_fma(D[26], m, L[6]);
+      L[7] = m2l_fma(D[28], m, L[7]);
+      L[8] = m2l_fma(D[29], m, L[8]);
+      L[9] = m2l_fma(D[34], m, L[9]);
+      L[10] = m2l_fma(D[37], m, L[10]);
+      L[11] = m2l_fma(D[38], m, L[11]);
+      L[12] = m2l_fma(D[40], m, L[12]);
+      L[13] = m2l_fma(D[41], m, L[13]);
+      L[14] = m2l_fma(D[43], m, L[14]);
+      L[15] = m2l_fma(D[44], m, L[15]);
+      L[16] = m2l_fma(D[49], m, L[16]);
+      L[17] = m2l_fma(D[52], m, L[17]);
+      L[18] = m2l_fma(D[53], m, L[18]);
+      L[19] = m2l_fma(D[55], m, L[19]);
+      L[20] = m2l_fma(D[56], m, L[20]);
+      L[21] = m2l_fma(D[58], m, L[21]);
+      L[22] = m2l_fma(D[59], m, L[22]);
+      L[23] = m2l_fma(D[61], m, L[23]);
+      L[24] = m2l_fma(D[62], m, L[24]);
     }
-    { const float m = -__ldg(Mr + 13) * rp;
-      L[1] = fmaf(D[23], m, L[1]);
-      L[2] = fmaf(D[26], m, L[2]);
-      L[3] = fmaf(D[27], m, L[3]);
-      L[4] = fmaf(D[35], m, L[4]);
-      L[5] = fmaf(D[38], m, L[5]);
-      L[6] = fmaf(D[39], m, L[6]);
-      L[7] = fmaf(D[41], m, L[7]);
-      L[8] = fmaf(D[42], m, L[8]);
-      L[9] = fmaf(D[50], m, L[9]);
-      L[10] = fmaf(D[53], m, L[10]);
-      L[11] = fmaf(D[54], m, L[11]);
-      L[12] = fmaf(D[56], m, L[12]);
-      L[13] = fmaf(D[57], m, L[13]);
-      L[14] = fmaf(D[59], m, L[14]);
-      L[15] = fmaf(D[60], m, L[15]);
-    }
-    { const float m = -__ldg(Mr + 14) * rp;
-      L[1] = fmaf(D[25], m, L[1]);
-      L[2] = fmaf(D[28], m, L[2]);
-      L[3] = fmaf(D[29], m, L[3]);
-      L[4] = fmaf(D[37], m, L[4]);
-      L[5] = fmaf(D[40], m, L[5]);
-      L[6] = fmaf(D[41], m, L[6]);
-      L[7] = fmaf(D[43], m, L[7]);
-      L[8] = fmaf(D[44], m, L[8]);
-      L[9] = fmaf(D[52], m, L[9]);
-      L[10] = fmaf(D[55], m, L[10]);
-      L[11] = fmaf(D[56], m, L[11]);
-      L[12] = fmaf(D[58], m, L[12]);
-      L[13] = fmaf(D[59], m, L[13]);
-      L[14] = fmaf(D[61], m, L[14]);
-      L[15] = fmaf(D[62], m, L[15]);
-    }
-    { const float m = -__ldg(Mr + 15) * rp;
-      L[1] = fmaf(D[26], m, L[1]);
-      L[2] = fmaf(D[29], m, L[2]);
-      L[3] = fmaf(D[30], m, L[3]);
-      L[4] = fmaf(D[38], m, L[4]);
-      L[5] = fmaf(D[41], m, L[5]);
-      L[6] = fmaf(D[42], m, L[6]);
-      L[7] = fmaf(D[44], m, L[7]);
-      L[8] = fmaf(D[45], m, L[8]);
-      L[9] = fmaf(D[53], m, L[9]);
-      L[10] = fmaf(D[56], m, L[10]);
-      L[11] = fmaf(D[57], m, L[11]);
-      L[12] = fmaf(D[59], m, L[12]);
-      L[13] = fmaf(D[60], m, L[13]);
-      L[14] = fmaf(D[62], m, L[14]);
-      L[15] = fmaf(D[63], m, L[15]);
-    }
-    rp *= rho;
-    { const float m = __ldg(Mr + 16) * rp;
-      L[1] = fmaf(D[31], m, L[1]);
-      L[2] = fmaf(D[32], m, L[2]);
-      L[3] = fmaf(D[33], m, L[3]);
-      L[4] = fmaf(D[46], m, L[4]);
-      L[5] = fmaf(D[47], m, L[5]);
-      L[6] = fmaf(D[48], m, L[6]);
-      L[7] = fmaf(D[49], m, L[7]);
-      L[8] = fmaf(D[50], m, L[8]);
-    }
-    { const float m = __ldg(Mr + 17) * rp;
-      L[1] = fmaf(D[32], m, L[1]);
-      L[2] = fmaf(D[34], m, L[2]);
-      L[3] = fmaf(D[35], m, L[3]);
-      L[4] = fmaf(D[47], m, L[4]);
-      L[5] = fmaf(D[49], m, L[5]);
-      L[6] = fmaf(D[50], m, L[6]);
-      L[7] = fmaf(D[52], m, L[7]);
-      L[8] = fmaf(D[53], m, L[8]);
-    }
-    { const float m = __ldg(Mr + 18) * rp;
-      L[1] = fmaf(D[33], m, L[1]);
-      L[2] = fmaf(D[35], m, L[2]);
-      L[3] = fmaf(D[36], m, L[3]);
-      L[4] = fmaf(D[48], m, L[4]);
-      L[5] = fmaf(D[50], m, L[5]);
-      L[6] = fmaf(D[51], m, L[6]);
-      L[7] = fmaf(D[53], m, L[7]);
-      L[8] = fmaf(D[54], m, L[8]);
-    }
-    { const float m = __ldg(Mr + 19) * rp;
-      L[1] = fmaf(D[34], m, L[1]);
-      L[2] = fmaf(D[37], m, L[2]);
-      L[3] = fmaf(D[38], m, L[3]);
-      L[4] = fmaf(D[49], m, L[4]);
-      L[5] = fmaf(D[52], m, L[5]);
-      L[6] = fmaf(D[53], m, L[6]);
-      L[7] = fmaf(D[55], m, L[7]);
-      L[8] = fmaf(D[56], m, L[8]);
-    }
-    { const float m = __ldg(Mr + 20) * rp;
-      L[1] = fmaf(D[35], m, L[1]);
-      L[2] = fmaf(D[38], m, L[2]);
-      L[3] = fmaf(D[39], m, L[3]);
-      L[4] = fmaf(D[50], m, L[4]);
-      L[5] = fmaf(D[53], m, L[5]);
-      L[6] = fmaf(D[54], m, L[6]);
-      L[7] = fmaf(D[56], m, L[7]);
-      L[8] = fmaf(D[57], m, L[8]);
-    }
-    { const float m = __ldg(Mr + 21) * rp;
-      L[1] = fmaf(D[37], m, L[1]);
-      L[2] = fmaf(D[40], m, L[2]);
-      L[3] = fmaf(D[41], m, L[3]);
-      L[4] = fmaf(D[52], m, L[4]);
-      L[5] = fmaf(D[55], m, L[5]);
-      L[6] = fmaf(D[56], m, L[6]);
-      L[7] = fmaf(D[58], m, L[7]);
-      L[8] = fmaf(D[59], m, L[8]);
-    }
-    { const float m = __ldg(Mr + 22) * rp;
-      L[1] = fmaf(D[38], m, L[1]);
-      L[2] = fmaf(D[41], m, L[2]);
-      L[3] = fmaf(D[42], m, L[3]);
-      L[4] = fmaf(D[53], m, L[4]);
-      L[5] = fmaf(D[56], m, L[5]);
-      L[6] = fmaf(D[57], m, L[6]);
-      L[7] = fmaf(D[59], m, L[7]);
-      L[8] = fmaf(D[60], m, L[8]);
-    }
-    { const float m = __ldg(Mr + 23) * rp;
-      L[1] = fmaf(D[40], m, L[1]);
-      L[2] = fmaf(D[43], m, L[2]);
-      L[3] = fmaf(D[44], m, L[3]);
-      L[4] = fmaf(D[55], m, L[4]);
-      L[5] = fmaf(D[58], m, L[5]);
-      L[6] = fmaf(D[59], m, L[6]);
-      L[7] = fmaf(D[61], m, L[7]);
-      L[8] = fmaf(D[62], m, L[8]);
-    }
-    { const float m = __ldg(Mr + 24) * rp;
-      L[1] = fmaf(D[41], m, L[1]);
-      L[2] = fmaf(D[44], m, L[2]);
-      L[3] = fmaf(D[45], m, L[3]);
-      L[4] = fmaf(D[56], m, L[4]);
-      L[5] = fmaf(D[59], m, L[5]);
-      L[6] = fmaf(D[60], m, L[6]);
-      L[7] = fmaf(D[62], m, L[7]);
-      L[8] = fmaf(D[63], m, L[8]);
+    { const T m = __ldg(Mr + 8) * rp;
+      L[1] = m2l_fma(D[14], m, L[1]);
+      L[2] = m2l_fma(D[17], m, L[2]);
+      L[3] = m2l_fma(D[18], m, L[3]);
+      L[4] = m2l_fma(D[23], m, L[4]);
+      L[5] = m2l_fma(D[26], m, L[5]);
+      L[6] = m2l_fma(D[27], m, L[6]);
+      L[7] = m2l_fma(D[29], m, L[7]);
+      L[8] = m2l_fma(D[30], m, L[8]);
+      L[9] = m2l_fma(D[35], m, L[9]);
+      L[10] = m2l_fma(D[38], m, L[10]);
+      L[11] = m2l_fma(D[39], m, L[11]);
+      L[12] = m2l_fma(D[41], m, L[12]);
+      L[13] = m2l_fma(D[42], m, L[13]);
+      L[14] = m2l_fma(D[44], m, L[14]);
+      L[15] = m2l_fma(D[45], m, L[15]);
+      L[16] = m2l_fma(D[50], m, L[16]);
+      L[17] = m2l_fma(D[53], m, L[17]);
+      L[18] = m2l_fma(D[54], m, L[18]);
+      L[19] = m2l_fma(D[56], m, L[19]);
+      L[20] = m2l_fma(D[57], m, L[20]);
+      L[21] = m2l_fma(D[59], m, L[21]);
+      L[22] = m2l_fma(D[60], m, L[22]);
+      L[23] = m2l_fma(D[62], m, L[23]);
+      L[24] = m2l_fma(D[63], m, L[24]);
     }
     rp *= rho;
-    { const float m = -__ldg(Mr + 25) * rp;
-      L[1] = fmaf(D[46], m, L[1]);
-      L[2] = fmaf(D[47], m, L[2]);
-      L[3] = fmaf(D[48], m, L[3]);
+    { const T m = -__ldg(Mr + 9) * rp;
+      L[1] = m2l_fma(D[19], m, L[1]);
+      L[2] = m2l_fma(D[20], m, L[2]);
+      L[3] = m2l_fma(D[21], m, L[3]);
+      L[4] = m2l_fma(D[31], m, L[4]);
+      L[5] = m2l_fma(D[32], m, L[5]);
+      L[6] = m2l_fma(D[33], m, L[6]);
+      L[7] = m2l_fma(D[34], m, L[7]);
+      L[8] = m2l_fma(D[35], m, L[8]);
+      L[9] = m2l_fma(D[46], m, L[9]);
+      L[10] = m2l_fma(D[47], m, L[10]);
+      L[11] = m2l_fma(D[48], m, L[11]);
+      L[12] = m2l_fma(D[49], m, L[12]);
+      L[13] = m2l_fma(D[50], m, L[13]);
+      L[14] = m2l_fma(D[52], m, L[14]);
+      L[15] = m2l_fma(D[53], m, L[15]);
     }
-    { const float m = -__ldg(Mr + 26) * rp;
-      L[1] = fmaf(D[47], m, L[1]);
-      L[2] = fmaf(D[49], m, L[2]);
-      L[3] = fmaf(D[50], m, L[3]);
+    { const T m = -__ldg(Mr + 10) * rp;
+      L[1] = m2l_fma(D[20], m, L[1]);
+      L[2] = m2l_fma(D[22], m, L[2]);
+      L[3] = m2l_fma(D[23], m, L[3]);
+      L[4] = m2l_fma(D[32], m, L[4]);
+      L[5] = m2l_fma(D[34], m, L[5]);
+      L[6] = m2l_fma(D[35], m, L[6]);
+      L[7] = m2l_fma(D[37], m, L[7]);
+      L[8] = m2l_fma(D[38], m, L[8]);
+      L[9] = m2l_fma(D[47], m, L[9]);
+      L[10] = m2l_fma(D[49], m, L[10]);
+      L[11] = m2l_fma(D[50], m, L[11]);
+      L[12] = m2l_fma(D[52], m, L[12]);
+      L[13] = m2l_fma(D[53], m, L[13]);
+      L[14] = m2l_fma(D[55], m, L[14]);
+      L[15] = m2l_fma(D[56], m, L[15]);
     }
-    { const float m = -__ldg(Mr + 27) * rp;
-      L[1] = fmaf(D[48], m, L[1]);
-      L[2] = fmaf(D[50], m, L[2]);
-      L[3] = fmaf(D[51], m, L[3]);
+    { const T m = -__ldg(Mr + 11) * rp;
+      L[1] = m2l_fma(D[21], m, L[1]);
+      L[2] = m2l_fma(D[23], m, L[2]);
+      L[3] = m2l_fma(D[24], m, L[3]);
+      L[4] = m2l_fma(D[33], m, L[4]);
+      L[5] = m2l_fma(D[35], m, L[5]);
+      L[6] = m2l_fma(D[36], m, L[6]);
+      L[7] = m2l_fma(D[38], m, L[7]);
+      L[8] = m2l_fma(D[39], m, L[8]);
+      L[9] = m2l_fma(D[48], m, L[9]);
+      L[10] = m2l_fma(D[50], m, L[10]);
+      L[11] = m2l_fma(D[51], m, L[11]);
+      L[12] = m2l_fma(D[53], m, L[12]);
+      L[13] = m2l_fma(D[54], m, L[13]);
+      L[14] = m2l_fma(D[56], m, L[14]);
+      L[15] = m2l_fma(D[57], m, L[15]);
     }
-    { const float m = -__ldg(Mr + 28) * rp;
-      L[1] = fmaf(D[49], m, L[1]);
-      L[2] = fmaf(D[52], m, L[2]);
-      L[3] = fmaf(D[53], m, L[3]);
+    { const T m = -__ldg(Mr + 12) * rp;
+      L[1] = m2l_fma(D[22], m, L[1]);
+      L[2] = m2l_fma(D[25], m, L[2]);
+      L[3] = m2l_fma(D[26], m, L[3]);
+      L[4] = m2l_fma(D[34], m, L[4]);
+      L[5] = m2l_fma(D[37], m, L[5]);
+      L[6] = m2l_fma(D[38], m, L[6]);
+      L[7] = m2l_fma(D[40], m, L[7]);
+      L[8] = m2l_fma(D[41], m, L[8]);
+      L[9] = m2l_fma(D[49], m, L[9]);
+      L[10] = m2l_fma(D[52], m, L[10]);
+      L[11] = m2l_fma(D[53], m, L[11]);
+      L[12] = m2l_fma(D[55], m, L[12]);
+      L[13] = m2l_fma(D[56], m, L[13]);
+      L[14] = m2l_fma(D[58], m, L[14]);
+      L[15] = m2l_fma(D[59], m, L[15]);
     }
-    { const float m = -__ldg(Mr + 29) * rp;
-      L[1] = fmaf(D[50], m, L[1]);
-      L[2] = fmaf(D[53], m, L[2]);
-      L[3] = fmaf(D[54], m, L[3]);
+    { const T m = -__ldg(Mr + 13) * rp;
+      L[1] = m2l_fma(D[23], m, L[1]);
+      L[2] = m2l_fma(D[26], m, L[2]);
+      L[3] = m2l_fma(D[27], m, L[3]);
+      L[4] = m2l_fma(D[35], m, L[4]);
+      L[5] = m2l_fma(D[38], m, L[5]);
+      L[6] = m2l_fma(D[39], m, L[6]);
+      L[7] = m2l_fma(D[41], m, L[7]);
+      L[8] = m2l_fma(D[42], m, L[8]);
+      L[9] = m2l_fma(D[50], m, L[9]);
+      L[10] = m2l_fma(D[53], m, L[10]);
+      L[11] = m2l_fma(D[54], m, L[11]);
+      L[12] = m2l_fma(D[56], m, L[12]);
+      L[13] = m2l_fma(D[57], m, L[13]);
+      L[14] = m2l_fma(D[59], m, L[14]);
+      L[15] = m2l_fma(D[60], m, L[15]);
     }
-    { const float m = -__ldg(Mr + 30) * rp;
-      L[1] = fmaf(D[52], m, L[1]);
-      L[2] = fmaf(D[55], m, L[2]);
-      L[3] = fmaf(D[56], m, L[3]);
+    { const T m = -__ldg(Mr + 14) * rp;
+      L[1] = m2l_fma(D[25], m, L[1]);
+      L[2] = m2l_fma(D[28], m, L[2]);
+      L[3] = m2l_fma(D[29], m, L[3]);
+      L[4] = m2l_fma(D[37], m, L[4]);
+      L[5] = m2l_fma(D[40], m, L[5]);
+      L[6] = m2l_fma(D[41], m, L[6]);
+      L[7] = m2l_fma(D[43], m, L[7]);
+      L[8] = m2l_fma(D[44], m, L[8]);
+      L[9] = m2l_fma(D[52], m, L[9]);
+      L[10] = m2l_fma(D[55], m, L[10]);
+      L[11] = m2l_fma(D[56], m, L[11]);
+      L[12] = m2l_fma(D[58], m, L[12]);
+      L[13] = m2l_fma(D[59], m, L[13]);
+      L[14] = m2l_fma(D[61], m, L[14]);
+      L[15] = m2l_fma(D[62], m, L[15]);
     }
-    { const float m = -__ldg(Mr + 31) * rp;
-      L[1] = fmaf(D[53], m, L[1]);
-      L[2] = fmaf(D[56], m, L[2]);
-      L[3] = fmaf(D[57], m, L[3]);
+    { const T m = -__ldg(Mr + 15) * rp;
+      L[1] = m2l_fma(D[26], m, L[1]);
+      L[2] = m2l_fma(D[29], m, L[2]);
+      L[3] = m2l_fma(D[30], m, L[3]);
+      L[4] = m2l_fma(D[38], m, L[4]);
+      L[5] = m2l_fma(D[41], m, L[5]);
+      L[6] = m2l_fma(D[42], m, L[6]);
+      L[7] = m2l_fma(D[44], m, L[7]);
+      L[8] = m2l_fma(D[45], m, L[8]);
+      L[9] = m2l_fma(D[53], m, L[9]);
+      L[10] = m2l_fma(D[56], m, L[10]);
+      L[11] = m2l_fma(D[57], m, L[11]);
+      L[12] = m2l_fma(D[59], m, L[12]);
+      L[13] = m2l_fma(D[60], m, L[13]);
+      L[14] = m2l_fma(D[62], m, L[14]);
+      L[15] = m2l_fma(D[63], m, L[15]);
     }
-    { const float m = -__ldg(Mr + 32) * rp;
-      L[1] = fmaf(D[55], m, L[1]);
-      L[2] = fmaf(D[58], m, L[2]);
-      L[3] = fmaf(D[59], m, L[3]);
+    rp *= rho;
+    { const T m = __ldg(Mr + 16) * rp;
+      L[1] = m2l_fma(D[31], m, L[1]);
+      L[2] = m2l_fma(D[32], m, L[2]);
+      L[3] = m2l_fma(D[33], m, L[3]);
+      L[4] = m2l_fma(D[46], m, L[4]);
+      L[5] = m2l_fma(D[47], m, L[5]);
+      L[6] = m2l_fma(D[48], m, L[6]);
+      L[7] = m2l_fma(D[49], m, L[7]);
+      L[8] = m2l_fma(D[50], m, L[8]);
     }
-    { const float m = -__ldg(Mr + 33) * rp;
-      L[1] = fmaf(D[56], m, L[1]);
-      L[2] = fmaf(D[59], m, L[2]);
-      L[3] = fmaf(D[60], m, L[3]);
+    { const T m = __ldg(Mr + 17) * rp;
+      L[1] = m2l_fma(D[32], m, L[1]);
+      L[2] = m2l_fma(D[34], m, L[2]);
+      L[3] = m2l_fma(D[35], m, L[3]);
+      L[4] = m2l_fma(D[47], m, L[4]);
+      L[5] = m2l_fma(D[49], m, L[5]);
+      L[6] = m2l_fma(D[50], m, L[6]);
+      L[7] = m2l_fma(D[52], m, L[7]);
+      L[8] = m2l_fma(D[53], m, L[8]);
     }
-    { const float m = -__ldg(Mr + 34) * rp;
-      L[1] = fmaf(D[58], m, L[1]);
-      L[2] = fmaf(D[61], m, L[2]);
-      L[3] = fmaf(D[62], m, L[3]);
+    { const T m = __ldg(Mr + 18) * rp;
+      L[1] = m2l_fma(D[33], m, L[1]);
+      L[2] = m2l_fma(D[35], m, L[2]);
+      L[3] = m2l_fma(D[36], m, L[3]);
+      L[4] = m2l_fma(D[48], m, L[4]);
+      L[5] = m2l_fma(D[50], m, L[5]);
+      L[6] = m2l_fma(D[51], m, L[6]);
+      L[7] = m2l_fma(D[53], m, L[7]);
+      L[8] = m2l_fma(D[54], m, L[8]);
     }
-    { const float m = -__ldg(Mr + 35) * rp;
-      L[1] = fmaf(D[59], m, L[1]);
-      L[2] = fmaf(D[62], m, L[2]);
-      L[3] = fmaf(D[63], m, L[3]);
+    { const T m = __ldg(Mr + 19) * rp;
+      L[1] = m2l_fma(D[34], m, L[1]);
+      L[2] = m2l_fma(D[37], m, L[2]);
+      L[3] = m2l_fma(D[38], m, L[3]);
+      L[4] = m2l_fma(D[49], m, L[4]);
+      L[5] = m2l_fma(D[52], m, L[5]);
+      L[6] = m2l_fma(D[53], m, L[6]);
+      L[7] = m2l_fma(D[55], m, L[7]);
+      L[8] = m2l_fma(D[56], m, L[8]);
+    }
+    { const T m = __ldg(Mr + 20) * rp;
+      L[1] = m2l_fma(D[35], m, L[1]);
+      L[2] = m2l_fma(D[38], m, L[2]);
+      L[3] = m2l_fma(D[39], m, L[3]);
+      L[4] = m2l_fma(D[50], m, L[4]);
+      L[5] = m2l_fma(D[53], m, L[5]);
+      L[6] = m2l_fma(D[54], m, L[6]);
+      L[7] = m2l_fma(D[56], m, L[7]);
+      L[8] = m2l_fma(D[57], m, L[8]);
+    }
+    { const T m = __ldg(Mr + 21) * rp;
+      L[1] = m2l_fma(D[37], m, L[1]);
+      L[2] = m2l_fma(D[40], m, L[2]);
+      L[3] = m2l_fma(D[41], m, L[3]);
+      L[4] = m2l_fma(D[52], m, L[4]);
+      L[5] = m2l_fma(D[55], m, L[5]);
+      L[6] = m2l_fma(D[56], m, L[6]);
+      L[7] = m2l_fma(D[58], m, L[7]);
+      L[8] = m2l_fma(D[59], m, L[8]);
+    }
+    { const T m = __ldg(Mr + 22) * rp;
+      L[1] = m2l_fma(D[38], m, L[1]);
+      L[2] = m2l_fma(D[41], m, L[2]);
+      L[3] = m2l_fma(D[42], m, L[3]);
+      L[4] = m2l_fma(D[53], m, L[4]);
+      L[5] = m2l_fma(D[56], m, L[5]);
+      L[6] = m2l_fma(D[57], m, L[6]);
+      L[7] = m2l_fma(D[59], m, L[7]);
+      L[8] = m2l_fma(D[60], m, L[8]);
+    }
+    { const T m = __ldg(Mr + 23) * rp;
+      L[1] = m2l_fma(D[40], m, L[1]);
+      L[2] = m2l_fma(D[43], m, L[2]);
+      L[3] = m2l_fma(D[44], m, L[3]);
+      L[4] = m2l_fma(D[55], m, L[4]);
+      L[5] = m2l_fma(D[58], m, L[5]);
+      L[6] = m2l_fma(D[59], m, L[6]);
+      L[7] = m2l_fma(D[61], m, L[7]);
+      L[8] = m2l_fma(D[62], m, L[8]);
+    }
+    { const T m = __ldg(Mr + 24) * rp;
+      L[1] = m2l_fma(D[41], m, L[1]);
+      L[2] = m2l_fma(D[44], m, L[2]);
+      L[3] = m2l_fma(D[45], m, L[3]);
+      L[4] = m2l_fma(D[56], m, L[4]);
+      L[5] = m2l_fma(D[59], m, L[5]);
+      L[6] = m2l_fma(D[60], m, L[6]);
+      L[7] = m2l_fma(D[62], m, L[7]);
+      L[8] = m2l_fma(D[63], m, L[8]);
+    }
+    rp *= rho;
+    { const T m = -__ldg(Mr + 25) * rp;
+      L[1] = m2l_fma(D[46], m, L[1]);
+      L[2] = m2l_fma(D[47], m, L[2]);
+      L[3] = m2l_fma(D[48], m, L[3]);
+    }
+    { const T m = -__ldg(Mr + 26) * rp;
+      L[1] = m2l_fma(D[47], m, L[1]);
+      L[2] = m2l_fma(D[49], m, L[2]);
+      L[3] = m2l_fma(D[50], m, L[3]);
+    }
+    { const T m = -__ldg(Mr + 27) * rp;
+      L[1] = m2l_fma(D[48], m, L[1]);
+      L[2] = m2l_fma(D[50], m, L[2]);
+      L[3] = m2l_fma(D[51], m, L[3]);
+    }
+    { const T m = -__ldg(Mr + 28) * rp;
+      L[1] = m2l_fma(D[49], m, L[1]);
+      L[2] = m2l_fma(D[52], m, L[2]);
+      L[3] = m2l_fma(D[53], m, L[3]);
+    }
+    { const T m = -__ldg(Mr + 29) * rp;
+      L[1] = m2l_fma(D[50], m, L[1]);
+      L[2] = m2l_fma(D[53], m, L[2]);
+      L[3] = m2l_fma(D[54], m, L[3]);
+    }
+    { const T m = -__ldg(Mr + 30) * rp;
+      L[1] = m2l_fma(D[52], m, L[1]);
+      L[2] = m2l_fma(D[55], m, L[2]);
+      L[3] = m2l_fma(D[56], m, L[3]);
+    }
+    { const T m = -__ldg(Mr + 31) * rp;
+      L[1] = m2l_fma(D[53], m, L[1]);
+      L[2] = m2l_fma(D[56], m, L[2]);
+      L[3] = m2l_fma(D[57], m, L[3]);
+    }
+    { const T m = -__ldg(Mr + 32) * rp;
+      L[1] = m2l_fma(D[55], m, L[1]);
+      L[2] = m2l_fma(D[58], m, L[2]);
+      L[3] = m2l_fma(D[59], m, L[3]);
+    }
+    { const T m = -__ldg(Mr + 33) * rp;
+      L[1] = m2l_fma(D[56], m, L[1]);
+      L[2] = m2l_fma(D[59], m, L[2]);
+      L[3] = m2l_fma(D[60], m, L[3]);
+    }
+    { const T m = -__ldg(Mr + 34) * rp;
+      L[1] = m2l_fma(D[58], m, L[1]);
+      L[2] = m2l_fma(D[61], m, L[2]);
+      L[3] = m2l_fma(D[62], m, L[3]);
+    }
+    { const T m = -__ldg(Mr + 35) * rp;
+      L[1] = m2l_fma(D[59], m, L[1]);
+      L[2] = m2l_fma(D[62], m, L[2]);
+      L[3] = m2l_fma(D[63], m, L[3]);
     }
 }
 
-__device__ __forceinline__ void m2l_acc_h_forces_6(const float (&D)[64], const float *__restrict__ Mr, float rho, float (&L)[49])
+template <class T> __device__ __forceinline__ void m2l_acc_h_forces_6(const T (&D)[64], const T *__restrict__ Mr, T rho, T (&L)[49])
 {
-    float rp = 1.0f;
-    { const float m = __ldg(Mr + 0) * rp;
-      L[1] = fmaf(D[1], m, L[1]);
-      L[2] = fmaf(D[2], m, L[2]);
-      L[3] = fmaf(D[3], m, L[3]);
-      L[4] = fmaf(D[4], m, L[4]);
-      L[5] = fmaf(D[5], m, L[5]);
-      L[6] = fmaf(D[6], m, L[6]);
-      L[7] = fmaf(D[7], m, L[7]);
-      L[8] = fmaf(D[8], m, L[8]);
-      L[9] = fmaf(D[10], m, L[9]);
-      L[10] = fmaf(D[11], m, L[10]);
-      L[11] = fmaf(D[12], m, L[11]);
-      L[12] = fmaf(D[13], m, L[12]);
-      L[13] = fmaf(D[14], m, L[13]);
-      L[14] = fmaf(D[16], m, L[14]);
-      L[15] = fmaf(D[17], m, L[15]);
-      L[16] = fmaf(D[19], m, L[16]);
-      L[17] = fmaf(D[20], m, L[17]);
-      L[18] = fmaf(D[21], m, L[18]);
-      L[19] = fmaf(D[22], m, L[19]);
-      L[20] = fmaf(D[23], m, L[20]);
-      L[21] = fmaf(D[25], m, L[21]);
-      L[22] = fmaf(D[26], m, L[22]);
-      L[23] = fmaf(D[28], m, L[23]);
-      L[24] = fmaf(D[29], m, L[24]);
-      L[25] = fmaf(D[31], m, L[25]);
-      L[26] = fmaf(D[32], m, L[26]);
-      L[27] = fmaf(D[33], m, L[27]);
-      L[28] = fmaf(D[34], m, L[28]);
-      L[29] = fmaf(D[35], m, L[29]);
-      L[30] = fmaf(D[37], m, L[30]);
-      L[31] = fmaf(D[38], m, L[31]);
-      L[32] = fmaf(D[40], m, L[32]);
-      L[33] = fmaf(D[41], m, L[33]);
-      L[34] = fmaf(D[43], m, L[34]);
-      L[35] = fmaf(D[44], m, L[35]);
-      L[36] = fmaf(D[46], m, L[36]);
-      L[37] = fmaf(D[47], m, L[37]);
-      L[38] = fmaf(D[48], m, L[38]);
-      L[39] = fmaf(D[49], m, L[39]);
-      L[40] = fmaf(D[50], m, L[40]);
-      L[41] = fmaf(D[52], m, L[41]);
-      L[42] = fmaf(D[53], m, L[42]);
-      L[43] = fmaf(D[55], m, L[43]);
-      L[44] = fmaf(D[56], m, L[44]);
-      L[45] = fmaf(D[58], m, L[45]);
-      L[46] = fmaf(D[59], m, L[46]);
-      L[47] = fmaf(D[61], m, L[47]);
-      L[48] = fmaf(D[62], m, L[48]);
+    T rp = T(1);
+    { const T m = __ldg(Mr + 0) * rp;
+      L[1] = m2l_fma(D[1], m, L[1]);
+      L[2] = m2l_fma(D[2], m, L[2]);
+      L[3] = m2l_fma(D[3], m, L[3]);
+      L[4] = m2l_fma(D[4], m, L[4]);
+      L[5] = m2l_fma(D[5], m, L[5]);
+      L[6] = m2l_fma(D[6], m, L[6]);
+      L[7] = m2l_fma(D[7], m, L[7]);
+      L[8] = m2l_fma(D[8], m, L[8]);
+      L[9] = m2l_fma(D[10], m, L[9]);
+      L[10] = m2l_fma(D[11], m, L[10]);
+      L[11] = m2l_fma(D[12], m, L[11]);
+      L[12] = m2l_fma(D[13], m, L[12]);
+      L[13] = m2l_fma(D[14], m, L[13]);
+      L[14] = m2l_fma(D[16], m, L[14]);
+      L[15] = m2l_fma(D[17], m, L[15]);
+      L[16] = m2l_fma(D[19], m, L[16]);
+      L[17] = m2l_fma(D[20], m, L[17]);
+      L[18] = m2l_fma(D[21], m, L[18]);
+      L[19] = m2l_fma(D[22], m, L[19]);
+      L[20] = m2l_fma(D[23], m, L[20]);
+      L[21] = m2l_fma(D[25], m, L[21]);
+      L[22] = m2l_fma(D[26], m, L[22]);
+      L[23] = m2l_fma(D[28], m, L[23]);
+      L[24] = m2l_fma(D[29], m, L[24]);
+      L[25] = m2l_fma(D[31], m, L[25]);
+      L[26] = m2l_fma(D[32], m, L[26]);
+      L[27] = m2l_fma(D[33], m, L[27]);
+      L[28] = m2l_fma(D[34], m, L[28]);
+      L[29] = m2l_fma(D[35], m, L[29]);
+      L[30] = m2l_fma(D[37], m, L[30]);
+      L[31] = m2l_fma(D[38], m, L[31]);
+      L[32] = m2l_fma(D[40], m, L[32]);
+      L[33] = m2l_fma(D[41], m, L[33]);
+      L[34] = m2l_fma(D[43], m, L[34]);
+      L[35] = m2l_fma(D[44], m, L[35]);
+      L[36] = m2l_fma(D[46], m, L[36]);
+      L[37] = m2l_fma(D[47], m, L[37]);
+      L[38] = m2l_fma(D[48], m, L[38]);
+      L[39] = m2l_fma(D[49], m, L[39]);
+      L[40] = m2l_fma(D[50], m, L[40]);
+      L[41] = m2l_fma(D[52], m, L[41]);
+      L[42] = m2l_fma(D[53], m, L[42]);
+      L[43] = m2l_fma(D[55], m, L[43]);
+      L[44] = m2l_fma(D[56], m, L[44]);
+      L[45] = m2l_fma(D[58], m, L[45]);
+      L[46] = m2l_fma(D[59], m, L[46]);
+      L[47] = m2l_fma(D[61], m, L[47]);
+      L[48] = m2l_fma(D[62], m, L[48]);
     }
     rp *= rho;
-    { const float m = -__ldg(Mr + 1) * rp;
-      L[1] = fmaf(D[4], m, L[1]);
-      L[2] = fmaf(D[5], m, L[2]);
-      L[3] = fmaf(D[6], m, L[3]);
-      L[4] = fmaf(D[10], m, L[4]);
-      L[5] = fmaf(D[11], m, L[5]);
-      L[6] = fmaf(D[12], m, L[6]);
-      L[7] = fmaf(D[13], m, L[7]);
-      L[8] = fmaf(D[14], m, L[8]);
-      L[9] = fmaf(D[19], m, L[9]);
-      L[10] = fmaf(D[20], m, L[10]);
-      L[11] = fmaf(D[21], m, L[11]);
-      L[12] = fmaf(D[22], m, L[12]);
-      L[13] = fmaf(D[23], m, L[13]);
-      L[14] = fmaf(D[25], m, L[14]);
-      L[15] = fmaf(D[26], m, L[15]);
-      L[16] = fmaf(D[31], m, L[16]);
-      L[17] = fmaf(D[32], m, L[17]);
-      L[18] = fmaf(D[33], m, L[18]);
-      L[19] = fmaf(D[34], m, L[19]);
-      L[20] = fmaf(D[35], m, L[20]);
-      L[21] = fmaf(D[37], m, L[21]);
-      L[22] = fmaf(D[38], m, L[22]);
-      L[23] = fmaf(D[40], m, L[23]);
-      L[24] = fmaf(D[41], m, L[24]);
-      L[25] = fmaf(D[46], m, L[25]);
-      L[26] = fmaf(D[47], m, L[26]);
-      L[27] = fmaf(D[48], m, L[27]);
-      L[28] = fmaf(D[49], m, L[28]);
-      L[29] = fmaf(D[50], m, L[29]);
-      L[30] = fmaf(D[52], m, L[30]);
-      L[31] = fmaf(D[53], m, L[31]);
-      L[32] = fmaf(D[55], m, L[32]);
-      L[33] = fmaf(D[56], m, L[33]);
-      L[34] = fmaf(D[58], m, L[34]);
-      L[35] = fmaf(D[59], m, L[35]);
+    { const T m = -__ldg(Mr + 1) * rp;
+      L[1] = m2l_fma(D[4], m, L[1]);
+      L[2] = m2l_fma(D[5], m, L[2]);
+      L[3] = m2l_fma(D[6], m, L[3]);
+      L[4] = m2l_fma(D[10], m, L[4]);
+      L[5] = m2l_fma(D[11], m, L[5]);
+      L[6] = m2l_fma(D[12], m, L[6]);
+      L[7] = m2l_fma(D[13], m, L[7]);
+      L[8] = m2l_fma(D[14], m, L[8]);
+      L[9] = m2l_fma(D[19], m, L[9]);
+      L[10] = m2l_fma(D[20], m, L[10]);
+      L[11] = m2l_fma(D[21], m, L[11]);
+      L[12] = m2l_fma(D[22], m, L[12]);
+      L[13] = m2l_fma(D[23], m, L[13]);
+      L[14] = m2l_fma(D[25], m, L[14]);
+      L[15] = m2l_fma(D[26], m, L[15]);
+      L[16] = m2l_fma(D[31], m, L[16]);
+      L[17] = m2l_fma(D[32], m, L[17]);
+      L[18] = m2l_fma(D[33], m, L[18]);
+      L[19] = m2l_fma(D[34], m, L[19]);
+      L[20] = m2l_fma(D[35], m, L[20]);
+      L[21] = m2l_fma(D[37], m, L[21]);
+      L[22] = m2l_fma(D[38], m, L[22]);
+      L[23] = m2l_fma(D[40], m, L[23]);
+      L[24] = m2l_fma(D[41], m, L[24]);
+      L[25] = m2l_fma(D[46], m, L[25]);
+      L[26] = m2l_fma(D[47], m, L[26]);
+      L[27] = m2l_fma(D[48], m, L[27]);
+      L[28] = m2l_fma(D[49], m, L[28]);
+      L[29] = m2l_fma(D[50], m, L[29]);
+      L[30] = m2l_fma(D[52], m, L[30]);
+      L[31] = m2l_fma(D[53], m, L[31]);
+      L[32] = m2l_fma(D[55], m, L[32]);
+      L[33] = m2l_fma(D[56], m, L[33]);
+      L[34] = m2l_fma(D[58], m, L[34]);
+      L[35] = m2l_fma(D[59], m, L[35]);
     }
-    { const float m = -__ldg(Mr + 2) * rp;
-      L[1] = fmaf(D[5], m, L[1]);
-      L[2] = fmaf(D[7], m, L[2]);
-      L[3] = fmaf(D[8], m, L[3]);
-      L[4] = fmaf(D[11], m, L[4]);
-      L[5] = fmaf(D[13], m, L[5]);
-      L[6] = fmaf(D[14], m, L[6]);
-      L[7] = fmaf(D[16], m, L[7]);
-      L[8] = fmaf(D[17], m, L[8]);
-      L[9] = fmaf(D[20], m, L[9]);
-      L[10] = fmaf(D[22], m, L[10]);
-      L[11] = fmaf(D[23], m, L[11]);
-      L[12] = fmaf(D[25], m, L[12]);
-      L[13] = fmaf(D[26], m, L[13]);
-      L[14] = fmaf(D[28], m, L[14]);
-      L[15] = fmaf(D[29], m, L[15]);
-      L[16] = fmaf(D[32], m, L[16]);
-      L[17] = fmaf(D[34], m, L[17]);
-      L[18] = fmaf(D[35], m, L[18]);
-      L[19] = fmaf(D[37], m, L[19]);
-      L[20] = fmaf(D[38], m, L[20]);
-      L[21] = fmaf(D[40], m, L[21]);
-      L[22] = fmaf(D[41], m, L[22]);
-      L[23] = fmaf(D[43], m, L[23]);
-      L[24] = fmaf(D[44], m, L[24]);
-      L[25] = fmaf(D[47], m, L[25]);
-      L[26] = fmaf(D[49], m, L[26]);
-      L[27] = fmaf(D[50], m, L[27]);
-      L[28] = fmaf(D[52], m, L[28]);
-      L[29] = fmaf(D[53], m, L[29]);
-      L[30] = fmaf(D[55], m, L[30]);
-      L[31] = fmaf(D[56], m, L[31]);
-      L[32] = fmaf(D[58], m, L[32]);
-      L[33] = fmaf(D[59], m, L[33]);
-      L[34] = fmaf(D[61], m, L[34]);
-      L[35] = fmaf(D[62], m, L[35]);
+    { const T m = -__ldg(Mr + 2) * rp;
+      L[1] = m2l_fma(D[5], m, L[1]);
+      L[2] = m2l_fma(D[7], m, L[2]);
+      L[3] = m2l_fma(D[8], m, L[3]);
+      L[4] = m2l_fma(D[11], m, L[4]);
+      L[5] = m2l_fma(D[13], m, L[5]);
+      L[6] = m2l_fma(D[14], m, L[6]);
+      L[7] = m2l_fma(D[16], m, L[7]);
+      L[8] = m2l_fma(D[17], m, L[8]);
+      L[9] = m2l_fma(D[20], m, L[9]);
+      L[10] = m2l_fma(D[22], m, L[10]);
+      L[11] = m2l_fma(D[23], m, L[11]);
+      L[12] = m2l_fma(D[25], m, L[12]);
+      L[13] = m2l_fma(D[26], m, L[13]);
+      L[14] = m2l_fma(D[28], m, L[14]);
+      L[15] = m2l_fma(D[29], m, L[15]);
+      L[16] = m2l_fma(D[32], m, L[16]);
+      L[17] = m2l_fma(D[34], m, L[17]);
+      L[18] = m2l_fma(D[35], m, L[18]);
+      L[19] = m2l_fma(D[37], m, L[19]);
+      L[20] = m2l_fma(D[38], m, L[20]);
+      L[21] = m2l_fma(D[40], m, L[21]);
+      L[22] = m2l_fma(D[41], m, L[22]);
+      L[23] = m2l_fma(D[43], m, L[23]);
+      L[24] = m2l_fma(D[44], m, L[24]);
+      L[25] = m2l_fma(D[47], m, L[25]);
+      L[26] = m2l_fma(D[49], m, L[26]);
+      L[27] = m2l_fma(D[50], m, L[27]);
+      L[28] = m2l_fma(D[52], m, L[28]);
+      L[29] = m2l_fma(D[53], m, L[29]);
+      L[30] = m2l_fma(D[55], m, L[30]);
+      L[31] = m2l_fma(D[56], m, L[31]);
+      L[32] = m2l_fma(D[58], m, L[32]);
+      L[33] = m2l_fma(D[59], m, L[33]);
+      L[34] = m2l_fma(D[61], m, L[34]);
+      L[35] = m2l_fma(D[62], m, L[35]);
     }
-    { const float m = -__ldg(Mr + 3) * rp;
-      L[1] = fmaf(D[6], m, L[1]);
-      L[2] = fmaf(D[8], m, L[2]);
-      L[3] = fmaf(D[9], m, L[3]);
-      L[4] = fmaf(D[12], m, L[4]);
-      L[5] = fmaf(D[14], m, L[5]);
-      L[6] = fmaf(D[15], m, L[6]);
-      L[7] = fmaf(D[17], m, L[7]);
-      L[8] = fmaf(D[18], m, L[8]);
-      L[9] = fmaf(D[21], m, L[9]);
-      L[10] = fmaf(D[23], m, L[10]);
-      L[11] = fmaf(D[24], m, L[11]);
-      L[12] = fmaf(D[26], m, L[12]);
-      L[13] = fmaf(D[27], m, L[13]);
-      L[14] = fmaf(D[29], m, L[14]);
-      L[15] = fmaf(D[30], m, L[15]);
-      L[16] = fmaf(D[33], m, L[16]);
-      L[17] = fmaf(D[35], m, L[17]);
-      L[18] = fmaf(D[36], m, L[18]);
-      L[19] = fmaf(D[38], m, L[19]);
-      L[20] = fmaf(D[39], m, L[20]);
-      L[21] = fmaf(D[41], m, L[21]);
-      L[22] = fmaf(D[42], m, L[22]);
-      L[23] = fmaf(D[44], m, L[23]);
-      L[24] = fmaf(D[45], m, L[24]);
-      L[25] = fmaf(D[48], m, L[25]);
-      L[26] = fmaf(D[50], m, L[26]);
-      L[27] = fmaf(D[51], m, L[27]);
-      L[28] = fmaf(D[53], m, L[28]);
-      L[29] = fmaf(D[54], m, L[29]);
-      L[30] = fmaf(D[56], m, L[30]);
-      L[31] = fmaf(D[57], m, L[31]);
-      L[32] = fmaf(D[59], m, L[32]);
-      L[33] = fmaf(D[60], m, L[33]);
-      L[34] = fmaf(D[62], m, L[34]);
-      L[35] = fmaf(D[63], m, L[35]);
-    }
-    rp *= rho;
-    { const float m = __ldg(Mr + 4) * rp;
-      L[1] = fmaf(D[10], m, L[1]);
-      L[2] = fmaf(D[11], m, L[2]);
-      L[3] = fmaf(D[12], m, L[3]);
-      L[4] = fmaf(D[19], m, L[4]);
-      L[5] = fmaf(D[20], m, L[5]);
-      L[6] = fmaf(D[21], m, L[6]);
-      L[7] = fmaf(D[22], m, L[7]);
-      L[8] = fmaf(D[23], m, L[8]);
-      L[9] = fmaf(D[31], m, L[9]);
-      L[10] = fmaf(D[32], m, L[10]);
-      L[11] = fmaf(D[33], m, L[11]);
-      L[12] = fmaf(D[34], m, L[12]);
-      L[13] = fmaf(D[35], m, L[13]);
-      L[14] = fmaf(D[37], m, L[14]);
-      L[15] = fmaf(D[38], m, L[15]);
-      L[16] = fmaf(D[46], m, L[16]);
-      L[17] = fmaf(D[47], m, L[17]);
-      L[18] = fmaf(D[48], m, L[18]);
-      L[19] = fmaf(D[49], m, L[19]);
-      L[20] = fmaf(D[50], m, L[20]);
-      L[21] = fmaf(D[52], m, L[21]);
-      L[22] = fmaf(D[53], m, L[22]);
-      L[23] = fmaf(D[55], m, L[23]);
-      L[24] = fmaf(D[56], m, L[24]);
-    }
-    { const float m = __ldg(Mr + 5) * rp;
-      L[1] = fmaf(D[11], m, L[1]);
-      L[2] = fmaf(D[13], m, L[2]);
-      L[3] = fmaf(D[14], m, L[3]);
-      L[4] = fmaf(D[20], m, L[4]);
-      L[5] = fmaf(D[22], m, L[5]);
-      L[6] = fmaf(D[23], m, L[6]);
-      L[7] = fmaf(D[25], m, L[7]);
-      L[8] = fmaf(D[26], m, L[8]);
-      L[9] = fmaf(D[32], m, L[9]);
-      L[10] = fmaf(D[34], m, L[10]);
-      L[11] = fmaf(D[35], m, L[11]);
-      L[12] = fmaf(D[37], m, L[12]);
-      L[13] = fmaf(D[38], m, L[13]);
-      L[14] = fmaf(D[40], m, L[14]);
-      L[15] = fmaf(D[41], m, L[15]);
-      L[16] = fmaf(D[47], m, L[16]);
-      L[17] = fmaf(D[49], m, L[17]);
-      L[18] = fmaf(D[50], m, L[18]);
-      L[19] = fmaf(D[52], m, L[19]);
-      L[20] = fmaf(D[53], m, L[20]);
-      L[21] = fmaf(D[55], m, L[21]);
-      L[22] = fmaf(D[56], m, L[22]);
-      L[23] = fmaf(D[58], m, L[23]);
-      L[24] = fmaf(D[59], m, L[24]);
-    }
-    { const float m = __ldg(Mr + 6) * rp;
-      L[1] = fmaf(D[12], m, L[1]);
-      L[2] = fmaf(D[14], m, L[2]);
-      L[3] = fmaf(D[15], m, L[3]);
-      L[4] = fmaf(D[21], m, L[4]);
-      L[5] = fmaf(D[23], m, L[5]);
-      L[6] = fmaf(D[24], m, L[6]);
-      L[7] = fmaf(D[26], m, L[7]);
-      L[8] = fmaf(D[27], m, L[8]);
-      L[9] = fmaf(D[33], m, L[9]);
-      L[10] = fmaf(D[35], m, L[10]);
-      L[11] = fmaf(D[36], m, L[11]);
-      L[12] = fmaf(D[38], m, L[12]);
-      L[13] = fmaf(D[39], m, L[13]);
-      L[14] = fmaf(D[41], m, L[14]);
-      L[15] = fmaf(D[42], m, L[15]);
-      L[16] = fmaf(D[48], m, L[16]);
-      L[17] = fmaf(D[50], m, L[17]);
-      L[18] = fmaf(D[51], m, L[18]);
-      L[19] = fmaf(D[53], m, L[19]);
-      L[20] = fmaf(D[54], m, L[20]);
-      L[21] = fmaf(D[56], m, L[21]);
-      L[22] = fmaf(D[57], m, L[22]);
-      L[23] = fmaf(D[59], m, L[23]);
-      L[24] = fmaf(D[60], m, L[24]);
-    }
-    { const float m = __ldg(Mr + 7) * rp;
-      L[1] = fmaf(D[13], m, L[1]);
-      L[2] = fmaf(D[16], m, L[2]);
-      L[3] = fmaf(D[17], m, L[3]);
-      L[4] = fmaf(D[22], m, L[4]);
-      L[5] = fmaf(D[25], m, L[5]);
-      L[6] = fmaf(D[26], m, L[6]);
-      L[7] = fmaf(D[28], m, L[7]);
-      L[8] = fmaf(D[29], m, L[8]);
-      L[9] = fmaf(D[34], m, L[9]);
-      L[10] = fmaf(D[37], m, L[10]);
-      L[11] = fmaf(D[38], m, L[11]);
-      L[12] = fmaf(D[40], m, L[12]);
-      L[13] = fmaf(D[41], m, L[13]);
-      L[14] = fmaf(D[43], m, L[14]);
-      L[15] = fmaf(D[44], m, L[15]);
-      L[16] = fmaf(D[49], m, L[16]);
-      L[17] = fmaf(D[52], m, L[17]);
-      L[18] = fmaf(D[53], m, L[18]);
-      L[19] = fmaf(D[55], m, L[19]);
-      L[20] = fmaf(D[56], m, L[20]);
-      L[21] = fmaf(D[58], m, L[21]);
-      L[22] = fmaf(D[59], m, L[22]);
-      L[23] = fmaf(D[61], m, L[23]);
-      L[24] = fmaf(D[62], m, L[24]);
-    }
-    { const float m = __ldg(Mr + 8) * rp;
-      L[1] = fmaf(D[14], m, L[1]);
-      L[2] = fmaf(D[17], m, L[2]);
-      L[3] = fmaf(D[18], m, L[3]);
-      L[4] = fmaf(D[23], m, L[4]);
-      L[5] = fmaf(D[26], m, L[5]);
-      L[6] = fmaf(D[27], m, L[6]);
-      L[7] = fmaf(D[29], m, L[7]);
-      L[8] = fmaf(D[30], m, L[8]);
-      L[9] = fmaf(D[35], m, L[9]);
-      L[10] = fmaf(D[38], m, L[10]);
-      L[11] = fmaf(D[39], m, L[11]);
-      L[12] = fmaf(D[41], m, L[12]);
-      L[13] = fmaf(D[42], m, L[13]);
-      L[14] = fmaf(D[44], m, L[14]);
-      L[15] = fmaf(D[45], m, L[15]);
-      L[16] = fmaf(D[50], m, L[16]);
-      L[17] = fmaf(D[53], m, L[17]);
-      L[18] = fmaf(D[54], m, L[18]);
-      L[19] = fmaf(D[56], m, L[19]);
-      L[20] = fmaf(D[57], m, L[20]);
-      L[21] = fmaf(D[59], m, L[21]);
-      L[22] = fmaf(D[60], m, L[22]);
-      L[23] = fmaf(D[62], m, L[23]);
-      L[24] = fmaf(D[63], m, L[24]);
+    { const T m = -__ldg(Mr + 3) * rp;
+      L[1] = m2l_fma(D[6], m, L[1]);
+      L[2] = m2l_fma(D[8], m, L[2]);
+      L[3] = m2l_fma(D[9], m, L[3]);
+      L[4] = m2l_fma(D[12], m, L[4]);
+      L[5] = m2l_fma(D[14], m, L[5]);
+      L[6] = m2l_fma(D[15], m, L[6]);
+      L[7] = m2l_fma(D[17], m, L[7]);
+      L[8] = m2l_fma(D[18], m, L[8]);
+      L[9] = m2l_fma(D[21], m, L[9]);
+      L[10] = m2l_fma(D[23], m, L[10]);
+      L[11] = m2l_fma(D[24], m, L[11]);
+      L[12] = m2l_fma(D[26], m, L[12]);
+      L[13] = m2l_fma(D[27], m, L[13]);
+      L[14] = m2l_fma(D[29], m, L[14]);
+      L[15] = m2l_fma(D[30], m, L[15]);
+      L[16] = m2l_fma(D[33], m, L[16]);
+      L[17] = m2l_fma(D[35], m, L[17]);
+      L[18] = m2l_fma(D[36], m, L[18]);
+      L[19] = m2l_fma(D[38], m, L[19]);
+      L[20] = m2l_fma(D[39], m, L[20]);
+      L[21] = m2l_fma(D[41], m, L[21]);
+      L[22] = m2l_fma(D[42], m, L[22]);
+      L[23] = m2l_fma(D[44], m, L[23]);
+      L[24] = m2l_fma(D[45], m, L[24]);
+      L[25] = m2l_fma(D[48], m, L[25]);
+      L[26] = m2l_fma(D[50], m, L[26]);
+      L[27] = m2l_fma(D[51], m, L[27]);
+      L[28] = m2l_fma(D[53], m, L[28]);
+      L[29] = m2l_fma(D[54], m, L[29]);
+      L[30] = m2l_fma(D[56], m, L[30]);
+      L[31] = m2l_fma(D[57], m, L[31]);
+      L[32] = m2l_fma(D[59], m, L[32]);
+      L[33] = m2l_fma(D[60], m, L[33]);
+      L[34] = m2l_fma(D[62], m, L[34]);
+      L[35] = m2l_fma(D[63], m, L[35]);
     }
     rp *= rho;
-    { const float m = -__ldg(Mr + 9) * rp;
-      L[1] = fmaf(D[19], m, L[1]);
-      L[2] = fmaf(D[20], m, L[2]);
-      L[3] = fmaf(D[21], m, L[3]);
-      L[4] = fmaf(D[31], m, L[4]);
-      L[5] = fmaf(D[32], m, L[5]);
-      L[6] = fmaf(D[33], m, L[6]);
-      L[7] = fmaf(D[34], m, L[7]);
-      L[8] = fmaf(D[35], m, L[8]);
-      L[9] = fmaf(D[46], m, L[9]);
-      L[10] = fmaf(D[47], m, L[10]);
-      L[11] = fmaf(D[48], m, L[11]);
-      L[12] = fmaf(D[49], m, L[12]);
-      L[13] = fmaf(D[50], m, L[13]);
-      L[14] = fmaf(D[52], m, L[14]);
-      L[15] = fmaf(D[53], m, L[15]);
+    { const T m = __ldg(Mr + 4) * rp;
+      L[1] = m2l_fma(D[10], m, L[1]);
+      L[2] = m2l_fma(D[11], m, L[2]);
+      L[3] = m2l_fma(D[12], m, L[3]);
+      L[4] = m2l_fma(D[19], m, L[4]);
+      L[5] = m2l_fma(D[20], m, L[5]);
+      L[6] = m2l_fma(D[21], m, L[6]);
+      L[7] = m2l_fma(D[22], m, L[7]);
+      L[8] = m2l_fma(D[23], m, L[8]);
+      L[9] = m2l_fma(D[31], m, L[9]);
+      L[10] = m2l_fma(D[32], m, L[10]);
+      L[11] = m2l_fma(D[33], m, L[11]);
+      L[12] = m2l_fma(D[34], m, L[12]);
+      L[13] = m2l_fma(D[35], m, L[13]);
+      L[14] = m2l_fma(D[37], m, L[14]);
+      L[15] = m2l_fma(D[38], m, L[15]);
+      L[16] = m2l_fma(D[46], m, L[16]);
+      L[17] = m2l_fma(D[47], m, L[17]);
+      L[18] = m2l_fma(D[48], m, L[18]);
+      L[19] = m2l_fma(D[49], m, L[19]);
+      L[20] = m2l_fma(D[50], m, L[20]);
+      L[21] = m2l_fma(D[52], m, L[21]);
+      L[22] = m2l_fma(D[53], m, L[22]);
+      L[23] = m2l_fma(D[55], m, L[23]);
+      L[24] = m2l_fma(D[56], m, L[24]);
     }
-    { const float m = -__ldg(Mr + 10) * rp;
-      L[1] = fmaf(D[20], m, L[1]);
-      L[2] = fmaf(D[22], m, L[2]);
-      L[3] = fmaf(D[23], m, L[3]);
-      L[4] = fmaf(D[32], m, L[4]);
-      L[5] = fmaf(D[34], m, L[5]);
-      L[6] = fmaf(D[35], m, L[6]);
-      L[7] = fmaf(D[37], m, L[7]);
-      L[8] = fmaf(D[38], m, L[8]);
-      L[9] = fmaf(D[47], m, L[9]);
-      L[10] = fmaf(D[49], m, L[10]);
-      L[11] = fmaf(D[50], m, L[11]);
-      L[12] = fmaf(D[52], m, L[12]);
-      L[13] = fmaf(D[53], m, L[13]);
-      L[14] = fmaf(D[55], m, L[14]);
-      L[15] = fmaf(D[56], m, L[15]);
+    { const T m = __ldg(Mr + 5) * rp;
+      L[1] = m2l_fma(D[11], m, L[1]);
+      L[2] = m2l_fma(D[13], m, L[2]);
+      L[3] = m2l_fma(D[14], m, L[3]);
+      L[4] = m2l_fma(D[20], m, L[4]);
+      L[5] = m2l_fma(D[22], m, L[5]);
+      L[6] = m2l_fma(D[23], m, L[6]);
+      L[7] = m2l_fma(D[25], m, L[7]);
+      L[8] = m2l_fma(D[26], m, L[8]);
+      L[9] = m2l_fma(D[32], m, L[9]);
+      L[10] = m2l_fma(D[34], m, L[10]);
+      L[11] = m2l_fma(D[35], m, L[11]);
+      L[12] = m2l_fma(D[37], m, L[12]);
+      L[13] = m2l_fma(D[38], m, L[13]);
+      L[14] = m2l_fma(D[40], m, L[14]);
+      L[15] = m2l_fma(D[41], m, L[15]);
+      L[16] = m2l_fma(D[47], m, L[16]);
+      L[17] = m2l_fma(D[49], m, L[17]);
+      L[18] = m2l_fma(D[50], m, L[18]);
+      L[19] = m2l_fma(D[52], m, L[19]);
+      L[20] = m2l_fma(D[53], m, L[20]);
+      L[21] = m2l_fma(D[55], m, L[21]);
+      L[22] = m2l_fma(D[56], m, L[22]);
+      L[23] = m2l_fma(D[58], m, L[23]);
+      L[24] = m2l_fma(D[59], m, L[24]);
     }
-    { const float m = -__ldg(Mr + 11) * rp;
-      L[1] = fmaf(D[21], m, L[1]);
-      L[2] = fmaf(D[23], m, L[2]);
-      L[3] = fmaf(D[24], m, L[3]);
-      L[4] = fmaf(D[33], m, L[4]);
-      L[5] = fmaf(D[35], m, L[5]);
-      L[6] = fmaf(D[36], m, L[6]);
-      L[7] = fmaf(D[38], m, L[7]);
-      L[8] = fmaf(D[39], m, L[8]);
-      L[9] = fmaf(D[48], m, L[9]);
-      L[10] = fmaf(D[50], m, L[10]);
-      L[11] = fmaf(D[51], m, L[11]);
-      L[12] = fmaf(D[53], m, L[12]);
-      L[13] = fmaf(D[54], m, L[13]);
-      L[14] = fmaf(D[56], m, L[14]);
-      L[15] = fmaf(D[57], m, L[15]);
+    { const T m = __ldg(Mr + 6) * rp;
+      L[1] = m2l_fma(D[12], m, L[1]);
+      L[2] = m2l_fma(D[14], m, L[2]);
+      L[3] = m2l_fma(D[15], m, L[3]);
+      L[4] = m2l_fma(D[21], m, L[4]);
+      L[5] = m2l_fma(D[23], m, L[5]);
+      L[6] = m2l_fma(D[24], m, L[6]);
+      L[7] = m2l_fma(D[26], m, L[7]);
+      L[8] = m2l_fma(D[27], m, L[8]);
+      L[9] = m2l_fma(D[33], m, L[9]);
+      L[10] = m2l_fma(D[35], m, L[10]);
+      L[11] = m2l_fma(D[36], m, L[11]);
+      L[12] = m2l_fma(D[38], m, L[12]);
+      L[13] = m2l_fma(D[39], m, L[13]);
+      L[14] = m2l_fma(D[41], m, L[14]);
+      L[15] = m2l_fma(D[42], m, L[15]);
+      L[16] = m2l_fma(D[48], m, L[16]);
+      L[17] = m2l_fma(D[50], m, L[17]);
+      L[18] = m2l_fma(D[51], m, L[18]);
+      L[19] = m2l_fma(D[53], m, L[19]);
+      L[20] = m2l_fma(D[54], m, L[20]);
+      L[21] = m2l_fma(D[56], m, L[21]);
+      L[22] = m2l_fma(D[57], m, L[22]);
+      L[23] = m2l_fma(D[59], m, L[23]);
+      L[24] = m2l_fma(D[60], m, L[24]);
     }
-    { const float m = -__ldg(Mr + 12) * rp;
-      L[1] = fmaf(D[22], m, L[1]);
-      L[2] = fmaf(D[25], m, L[2]);
-      L[3] = fmaf(D[26], m, L[3]);
-      L[4] = fmaf(D[34], m, L[4]);
-      L[5] = fmaf(D[37], m, L[5]);
-      L[6] = fmaf(D[38], m, L[6]);
-      L[7] = fmaf(D[40], m, L[7]);
-      L[8] = fmaf(D[41], m, L[8]);
-      L[9] = fmaf(D[49], m, L[9]);
-      L[10] = fmaf(D[52], m, L[10]);
-      L[11] = fmaf(D[53], m, L[11]);
-      L[12] = fmaf(D[55], m, L[12]);
-      L[13] = fmaf(D[56], m, L[13]);
-      L[14] = fmaf(D[58], m, L[14]);
-      L[15] = fmaf(D[59], m, L[15]);
+    { const T m = __ldg(Mr + 7) * rp;
+      L[1] = m2l_fma(D[13], m, L[1]);
+      L[2] = m2l_fma(D[16], m, L[2]);
+      L[3] = m2l_fma(D[17], m, L[3]);
+      L[4] = m2l_fma(D[22], m, L[4]);
+      L[5] = m2l_fma(D[25], m, L[5]);
+      L[6] = m2l_fma(D[26], m, L[6]);
+      L[7] = m2l_fma(D[28], m, L[7]);
+      L[8] = m2l_fma(D[29], m, L[8]);
+      L[9] = m2l_fma(D[34], m, L[9]);
+      L[10] = m2l_fma(D[37], m, L[10]);
+      L[11] = m2l_fma(D[38], m, L[11]);
+      L[12] = m2l_fma(D[40], m, L[12]);
+      L[13] = m2l_fma(D[41], m, L[13]);
+      L[14] = m2l_fma(D[43], m, L[14]);
+      L[15] = m2l_fma(D[44], m, L[15]);
+      L[16] = m2l_fma(D[49], m, L[16]);
+      L[17] = m2l_fma(D[52], m, L[17]);
+      L[18] = m2l_fma(D[53], m, L[18]);
+      L[19] = m2l_fma(D[55], m, L[19]);
+      L[20] = m2l_fma(D[56], m, L[20]);
+      L[21] = m2l_fma(D[58], m, L[21]);
+      L[22] = m2l_fma(D[59], m, L[22]);
+      L[23] = m2l_fma(D[61], m, L[23]);
+      L[24] = m2l_fma(D[62], m, L[24]);
     }
-    { const float m = -__ldg(Mr + 13) * rp;
-      L[1] = fmaf(D[23], m, L[1]);
-      L[2] = fmaf(D[26], m, L[2]);
-      L[3] = fmaf(D[27], m, L[3]);
-      L[4] = fmaf(D[35], m, L[4]);
-      L[5] = fmaf(D[38], m, L[5]);
-      L[6] = fmaf(D[39], m, L[6]);
-      L[7] = fmaf(D[41], m, L[7]);
-      L[8] = fmaf(D[42], m, L[8]);
-      L[9] = fmaf(D[50], m, L[9]);
-      L[10] = fmaf(D[53], m, L[10]);
-      L[11] = fmaf(D[54], m, L[11]);
-      L[12] = fmaf(D[56], m, L[12]);
-      L[13] = fmaf(D[57], m, L[13]);
-      L[14] = fmaf(D[59], m, L[14]);
-      L[15] = fmaf(D[60], m, L[15]);
-    }
-    { const float m = -__ldg(Mr + 14) * rp;
-      L[1] = fmaf(D[25], m, L[1]);
-      L[2] = fmaf(D[28], m, L[2]);
-      L[3] = fmaf(D[29], m, L[3]);
-      L[4] = fmaf(D[37], m, L[4]);
-      L[5] = fmaf(D[40], m, L[5]);
-      L[6] = fmaf(D[41], m, L[6]);
-      L[7] = fmaf(D[43], m, L[7]);
-      L[8] = fmaf(D[44], m, L[8]);
-      L[9] = fmaf(D[52], m, L[9]);
-      L[10] = fmaf(D[55], m, L[10]);
-      L[11] = fmaf(D[56], m, L[11]);
-      L[12] = fmaf(D[58], m, L[12]);
-      L[13] = fmaf(D[59], m, L[13]);
-      L[14] = fmaf(D[61], m, L[14]);
-      L[15] = fmaf(D[62], m, L[15]);
-    }
-    { const float m = -__ldg(Mr + 15) * rp;
-      L[1] = fmaf(D[26], m, L[1]);
-      L[2] = fmaf(D[29], m, L[2]);
-      L[3] = fmaf(D[30], m, L[3]);
-      L[4] = fmaf(D[38], m, L[4]);
-      L[5] = fmaf(D[41], m, L[5]);
-      L[6] = fmaf(D[42], m, L[6]);
-      L[7] = fmaf(D[44], m, L[7]);
-      L[8] = fmaf(D[45], m, L[8]);
-      L[9] = fmaf(D[53], m, L[9]);
-      L[10] = fmaf(D[56], m, L[10]);
-      L[11] = fmaf(D[57], m, L[11]);
-      L[12] = fmaf(D[59], m, L[12]);
-      L[13] = fmaf(D[60], m, L[13]);
-      L[14] = fmaf(D[62], m, L[14]);
-      L[15] = fmaf(D[63], m, L[15]);
-    }
-    rp *= rho;
-    { const float m = __ldg(Mr + 16) * rp;
-      L[1] = fmaf(D[31], m, L[1]);
-      L[2] = fmaf(D[32], m, L[2]);
-      L[3] = fmaf(D[33], m, L[3]);
-      L[4] = fmaf(D[46], m, L[4]);
-      L[5] = fmaf(D[47], m, L[5]);
-      L[6] = fmaf(D[48], m, L[6]);
-      L[7] = fmaf(D[49], m, L[7]);
-      L[8] = fmaf(D[50], m, L[8]);
-    }
-    { const float m = __ldg(Mr + 17) * rp;
-      L[1] = fmaf(D[32], m, L[1]);
-      L[2] = fmaf(D[34], m, L[2]);
-      L[3] = fmaf(D[35], m, L[3]);
-      L[4] = fmaf(D[47], m, L[4]);
-      L[5] = fmaf(D[49], m, L[5]);
-      L[6] = fmaf(D[50], m, L[6]);
-      L[7] = fmaf(D[52], m, L[7]);
-      L[8] = fmaf(D[53], m, L[8]);
-    }
-    { const float m = __ldg(Mr + 18) * rp;
-      L[1] = fmaf(D[33], m, L[1]);
-      L[2] = fmaf(D[35], m, L[2]);
-      L[3] = fmaf(D[36], m, L[3]);
-      L[4] = fmaf(D[48], m, L[4]);
-      L[5] = fmaf(D[50], m, L[5]);
-      L[6] = fmaf(D[51], m, L[6]);
-      L[7] = fmaf(D[53], m, L[7]);
-      L[8] = fmaf(D[54], m, L[8]);
-    }
-    { const float m = __ldg(Mr + 19) * rp;
-      L[1] = fmaf(D[34], m, L[1]);
-      L[2] = fmaf(D[37], m, L[2]);
-      L[3] = fmaf(D[38], m, L[3]);
-      L[4] = fmaf(D[49], m, L[4]);
-      L[5] = fmaf(D[52], m, L[5]);
-      L[6] = fmaf(D[53], m, L[6]);
-      L[7] = fmaf(D[55], m, L[7]);
-      L[8] = fmaf(D[56], m, L[8]);
-    }
-    { const float m = __ldg(Mr + 20) * rp;
-      L[1] = fmaf(D[35], m, L[1]);
-      L[2] = fmaf(D[38], m, L[2]);
-      L[3] = fmaf(D[39], m, L[3]);
-      L[4] = fmaf(D[50], m, L[4]);
-      L[5] = fmaf(D[53], m, L[5]);
-      L[6] = fmaf(D[54], m, L[6]);
-      L[7] = fmaf(D[56], m, L[7]);
-      L[8] = fmaf(D[57], m, L[8]);
-    }
-    { const float m = __ldg(Mr + 21) * rp;
-      L[1] = fmaf(D[37], m, L[1]);
-      L[2] = fmaf(D[40], m, L[2]);
-      L[3] = fmaf(D[41], m, L[3]);
-      L[4] = fmaf(D[52], m, L[4]);
-      L[5] = fmaf(D[55], m, L[5]);
-      L[6] = fmaf(D[56], m, L[6]);
-      L[7] = fmaf(D[58], m, L[7]);
-      L[8] = fmaf(D[59], m, L[8]);
-    }
-    { const float m = __ldg(Mr + 22) * rp;
-      L[1] = fmaf(D[38], m, L[1]);
-      L[2] = fmaf(D[41], m, L[2]);
-      L[3] = fmaf(D[42], m, L[3]);
-      L[4] = fmaf(D[53], m, L[4]);
-      L[5] = fmaf(D[56], m, L[5]);
-      L[6] = fmaf(D[57], m, L[6]);
-      L[7] = fmaf(D[59], m, L[7]);
-      L[8] = fmaf(D[60], m, L[8]);
-    }
-    { const float m = __ldg(Mr + 23) * rp;
-      L[1] = fmaf(D[40], m, L[1]);
-      L[2] = fmaf(D[43], m, L[2]);
-      L[3] = fmaf(D[44], m, L[3]);
-      L[4] = fmaf(D[55], m, L[4]);
-      L[5] = fmaf(D[58], m, L[5]);
-      L[6] = fmaf(D[59], m, L[6]);
-      L[7] = fmaf(D[61], m, L[7]);
-      L[8] = fmaf(D[62], m, L[8]);
-    }
-    { const float m = __ldg(Mr + 24) * rp;
-      L[1] = fmaf(D[41], m, L[1]);
-      L[2] = fmaf(D[44], m, L[2]);
-      L[3] = fmaf(D[45], m, L[3]);
-      L[4] = fmaf(D[56], m, L[4]);
-      L[5] = fmaf(D[59], m, L[5]);
-      L[6] = fmaf(D[60], m, L[6]);
-      L[7] = fmaf(D[62], m, L[7]);
-      L[8] = fmaf(D[63], m, L[8]);
+    { const T m = __ldg(Mr + 8) * rp;
+      L[1] = m2l_fma(D[14], m, L[1]);
+      L[2] = m2l_fma(D[17], m, L[2]);
+      L[3] = m2l_fma(D[18], m, L[3]);
+      L[4] = m2l_fma(D[23], m, L[4]);
+      L[5] = m2l_fma(D[26], m, L[5]);
+      L[6] = m2l_fma(D[27], m, L[6]);
+      L[7] = m2l_fma(D[29], m, L[7]);
+      L[8] = m2l_fma(D[30], m, L[8]);
+      L[9] = m2l_fma(D[35], m, L[9]);
+      L[10] = m2l_fma(D[38], m, L[10]);
+      L[11] = m2l_fma(D[39], m, L[11]);
+      L[12] = m2l_fma(D[41], m, L[12]);
+      L[13] = m2l_fma(D[42], m, L[13]);
+      L[14] = m2l_fma(D[44], m, L[14]);
+      L[15] = m2l_fma(D[45], m, L[15]);
+      L[16] = m2l_fma(D[50], m, L[16]);
+      L[17] = m2l_fma(D[53], m, L[17]);
+      L[18] = m2l_fma(D[54], m, L[18]);
+      L[19] = m2l_fma(D[56], m, L[19]);
+      L[20] = m2l_fma(D[57], m, L[20]);
+      L[21] = m2l_fma(D[59], m, L[21]);
+      L[22] = m2l_fma(D[60], m, L[22]);
+      L[23] = m2l_fma(D[62], m, L[23]);
+      L[24] = m2l_fma(D[63], m, L[24]);
     }
     rp *= rho;
-    { const float m = -__ldg(Mr + 25) * rp;
-      L[1] = fmaf(D[46], m, L[1]);
-      L[2] = fmaf(D[47], m, L[2]);
-      L[3] = fmaf(D[48], m, L[3]);
+    { const T m = -__ldg(Mr + 9) * rp;
+      L[1] = m2l_fma(D[19], m, L[1]);
+      L[2] = m2l_fma(D[20], m, L[2]);
+      L[3] = m2l_fma(D[21], m, L[3]);
+      L[4] = m2l_fma(D[31], m, L[4]);
+      L[5] = m2l_fma(D[32], m, L[5]);
+      L[6] = m2l_fma(D[33], m, L[6]);
+      L[7] = m2l_fma(D[34], m, L[7]);
+      L[8] = m2l_fma(D[35], m, L[8]);
+      L[9] = m2l_fma(D[46], m, L[9]);
+      L[10] = m2l_fma(D[47], m, L[10]);
+      L[11] = m2l_fma(D[48], m, L[11]);
+      L[12] = m2l_fma(D[49], m, L[12]);
+      L[13] = m2l_fma(D[50], m, L[13]);
+      L[14] = m2l_fma(D[52], m, L[14]);
+      L[15] = m2l_fma(D[53], m, L[15]);
     }
-    { const float m = -__ldg(Mr + 26) * rp;
-      L[1] = fmaf(D[47], m, L[1]);
-      L[2] = fmaf(D[49], m, L[2]);
-      L[3] = fmaf(D[50], m, L[3]);
+    { const T m = -__ldg(Mr + 10) * rp;
+      L[1] = m2l_fma(D[20], m, L[1]);
+      L[2] = m2l_fma(D[22], m, L[2]);
+      L[3] = m2l_fma(D[23], m, L[3]);
+      L[4] = m2l_fma(D[32], m, L[4]);
+      L[5] = m2l_fma(D[34], m, L[5]);
+      L[6] = m2l_fma(D[35], m, L[6]);
+      L[7] = m2l_fma(D[37], m, L[7]);
+      L[8] = m2l_fma(D[38], m, L[8]);
+      L[9] = m2l_fma(D[47], m, L[9]);
+      L[10] = m2l_fma(D[49], m, L[10]);
+      L[11] = m2l_fma(D[50], m, L[11]);
+      L[12] = m2l_fma(D[52], m, L[12]);
+      L[13] = m2l_fma(D[53], m, L[13]);
+      L[14] = m2l_fma(D[55], m, L[14]);
+      L[15] = m2l_fma(D[56], m, L[15]);
     }
-    { const float m = -__ldg(Mr + 27) * rp;
-      L[1] = fmaf(D[48], m, L[1]);
-      L[2] = fmaf(D[50], m, L[2]);
-      L[3] = fmaf(D[51], m, L[3]);
+    { const T m = -__ldg(Mr + 11) * rp;
+      L[1] = m2l_fma(D[21], m, L[1]);
+      L[2] = m2l_fma(D[23], m, L[2]);
+      L[3] = m2l_fma(D[24], m, L[3]);
+      L[4] = m2l_fma(D[33], m, L[4]);
+      L[5] = m2l_fma(D[35], m, L[5]);
+      L[6] = m2l_fma(D[36], m, L[6]);
+      L[7] = m2l_fma(D[38], m, L[7]);
+      L[8] = m2l_fma(D[39], m, L[8]);
+      L[9] = m2l_fma(D[48], m, L[9]);
+      L[10] = m2l_fma(D[50], m, L[10]);
+      L[11] = m2l_fma(D[51], m, L[11]);
+      L[12] = m2l_fma(D[53], m, L[12]);
+      L[13] = m2l_fma(D[54], m, L[13]);
+      L[14] = m2l_fma(D[56], m, L[14]);
+      L[15] = m2l_fma(D[57], m, L[15]);
     }
-    { const float m = -__ldg(Mr + 28) * rp;
-      L[1] = fmaf(D[49], m, L[1]);
-      L[2] = fmaf(D[52], m, L[2]);
-      L[3] = fmaf(D[53], m, L[3]);
+    { const T m = -__ldg(Mr + 12) * rp;
+      L[1] = m2l_fma(D[22], m, L[1]);
+      L[2] = m2l_fma(D[25], m, L[2]);
+      L[3] = m2l_fma(D[26], m, L[3]);
+      L[4] = m2l_fma(D[34], m, L[4]);
+      L[5] = m2l_fma(D[37], m, L[5]);
+      L[6] = m2l_fma(D[38], m, L[6]);
+      L[7] = m2l_fma(D[40], m, L[7]);
+      L[8] = m2l_fma(D[41], m, L[8]);
+      L[9] = m2l_fma(D[49], m, L[9]);
+      L[10] = m2l_fma(D[52], m, L[10]);
+      L[11] = m2l_fma(D[53], m, L[11]);
+      L[12] = m2l_fma(D[55], m, L[12]);
+      L[13] = m2l_fma(D[56], m, L[13]);
+      L[14] = m2l_fma(D[58], m, L[14]);
+      L[15] = m2l_fma(D[59], m, L[15]);
     }
-    { const float m = -__ldg(Mr + 29) * rp;
-      L[1] = fmaf(D[50], m, L[1]);
-      L[2] = fmaf(D[53], m, L[2]);
-      L[3] = fmaf(D[54], m, L[3]);
+    { const T m = -__ldg(Mr + 13) * rp;
+      L[1] = m2l_fma(D[23], m, L[1]);
+      L[2] = m2l_fma(D[26], m, L[2]);
+      L[3] = m2l_fma(D[27], m, L[3]);
+      L[4] = m2l_fma(D[35], m, L[4]);
+      L[5] = m2l_fma(D[38], m, L[5]);
+      L[6] = m2l_fma(D[39], m, L[6]);
+      L[7] = m2l_fma(D[41], m, L[7]);
+      L[8] = m2l_fma(D[42], m, L[8]);
+      L[9] = m2l_fma(D[50], m, L[9]);
+      L[10] = m2l_fma(D[53], m, L[10]);
+      L[11] = m2l_fma(D[54], m, L[11]);
+      L[12] = m2l_fma(D[56], m, L[12]);
+      L[13] = m2l_fma(D[57], m, L[13]);
+      L[14] = m2l_fma(D[59], m, L[14]);
+      L[15] = m2l_fma(D[60], m, L[15]);
     }
-    { const float m = -__ldg(Mr + 30) * rp;
-      L[1] = fmaf(D[52], m, L[1]);
-      L[2] = fmaf(D[55], m, L[2]);
-      L[3] = fmaf(D[56], m, L[3]);
+    { const T m = -__ldg(Mr + 14) * rp;
+      L[1] = m2l_fma(D[25], m, L[1]);
+      L[2] = m2l_fma(D[28], m, L[2]);
+      L[3] = m2l_fma(D[29], m, L[3]);
+      L[4] = m2l_fma(D[37], m, L[4]);
+      L[5] = m2l_fma(D[40], m, L[5]);
+      L[6] = m2l_fma(D[41], m, L[6]);
+      L[7] = m2l_fma(D[43], m, L[7]);
+      L[8] = m2l_fma(D[44], m, L[8]);
+      L[9] = m2l_fma(D[52], m, L[9]);
+      L[10] = m2l_fma(D[55], m, L[10]);
+      L[11] = m2l_fma(D[56], m, L[11]);
+      L[12] = m2l_fma(D[58], m, L[12]);
+      L[13] = m2l_fma(D[59], m, L[13]);
+      L[14] = m2l_fma(D[61], m, L[14]);
+      L[15] = m2l_fma(D[62], m, L[15]);
     }
-    { const float m = -__ldg(Mr + 31) * rp;
-      L[1] = fmaf(D[53], m, L[1]);
-      L[2] = fmaf(D[56], m, L[2]);
-      L[3] = fmaf(D[57], m, L[3]);
+    { const T m = -__ldg(Mr + 15) * rp;
+      L[1] = m2l_fma(D[26], m, L[1]);
+      L[2] = m2l_fma(D[29], m, L[2]);
+      L[3] = m2l_fma(D[30], m, L[3]);
+      L[4] = m2l_fma(D[38], m, L[4]);
+      L[5] = m2l_fma(D[41], m, L[5]);
+      L[6] = m2l_fma(D[42], m, L[6]);
+      L[7] = m2l_fma(D[44], m, L[7]);
+      L[8] = m2l_fma(D[45], m, L[8]);
+      L[9] = m2l_fma(D[53], m, L[9]);
+      L[10] = m2l_fma(D[56], m, L[10]);
+      L[11] = m2l_fma(D[57], m, L[11]);
+      L[12] = m2l_fma(D[59], m, L[12]);
+      L[13] = m2l_fma(D[60], m, L[13]);
+      L[14] = m2l_fma(D[62], m, L[14]);
+      L[15] = m2l_fma(D[63], m, L[15]);
     }
-    { const float m = -__ldg(Mr + 32) * rp;
-      L[1] = fmaf(D[55], m, L[1]);
-      L[2] = fmaf(D[58], m, L[2]);
-      L[3] = fmaf(D[59], m, L[3]);
+    rp *= rho;
+    { const T m = __ldg(Mr + 16) * rp;
+      L[1] = m2l_fma(D[31], m, L[1]);
+      L[2] = m2l_fma(D[32], m, L[2]);
+      L[3] = m2l_fma(D[33], m, L[3]);
+      L[4] = m2l_fma(D[46], m, L[4]);
+      L[5] = m2l_fma(D[47], m, L[5]);
+      L[6] = m2l_fma(D[48], m, L[6]);
+      L[7] = m2l_fma(D[49], m, L[7]);
+      L[8] = m2l_fma(D[50], m, L[8]);
     }
-    { const float m = -__ldg(Mr + 33) * rp;
-      L[1] = fmaf(D[56], m, L[1]);
-      L[2] = fmaf(D[59], m, L[2]);
-      L[3] = fmaf(D[60], m, L[3]);
+    { const T m = __ldg(Mr + 17) * rp;
+      L[1] = m2l_fma(D[32], m, L[1]);
+      L[2] = m2l_fma(D[34], m, L[2]);
+      L[3] = m2l_fma(D[35], m, L[3]);
+      L[4] = m2l_fma(D[47], m, L[4]);
+      L[5] = m2l_fma(D[49], m, L[5]);
+      L[6] = m2l_fma(D[50], m, L[6]);
+      L[7] = m2l_fma(D[52], m, L[7]);
+      L[8] = m2l_fma(D[53], m, L[8]);
     }
-    { const float m = -__ldg(Mr + 34) * rp;
-      L[1] = fmaf(D[58], m, L[1]);
-      L[2] = fmaf(D[61], m, L[2]);
-      L[3] = fmaf(D[62], m, L[3]);
+    { const T m = __ldg(Mr + 18) * rp;
+      L[1] = m2l_fma(D[33], m, L[1]);
+      L[2] = m2l_fma(D[35], m, L[2]);
+      L[3] = m2l_fma(D[36], m, L[3]);
+      L[4] = m2l_fma(D[48], m, L[4]);
+      L[5] = m2l_fma(D[50], m, L[5]);
+      L[6] = m2l_fma(D[51], m, L[6]);
+      L[7] = m2l_fma(D[53], m, L[7]);
+      L[8] = m2l_fma(D[54], m, L[8]);
     }
-    { const float m = -__ldg(Mr + 35) * rp;
-      L[1] = fmaf(D[59], m, L[1]);
-      L[2] = fmaf(D[62], m, L[2]);
-      L[3] = fmaf(D[63], m, L[3]);
+    { const T m = __ldg(Mr + 19) * rp;
+      L[1] = m2l_fma(D[34], m, L[1]);
+      L[2] = m2l_fma(D[37], m, L[2]);
+      L[3] = m2l_fma(D[38], m, L[3]);
+      L[4] = m2l_fma(D[49], m, L[4]);
+      L[5] = m2l_fma(D[52], m, L[5]);
+      L[6] = m2l_fma(D[53], m, L[6]);
+      L[7] = m2l_fma(D[55], m, L[7]);
+      L[8] = m2l_fma(D[56], m, L[8]);
+    }
+    { const T m = __ldg(Mr + 20) * rp;
+      L[1] = m2l_fma(D[35], m, L[1]);
+      L[2] = m2l_fma(D[38], m, L[2]);
+      L[3] = m2l_fma(D[39], m, L[3]);
+      L[4] = m2l_fma(D[50], m, L[4]);
+      L[5] = m2l_fma(D[53], m, L[5]);
+      L[6] = m2l_fma(D[54], m, L[6]);
+      L[7] = m2l_fma(D[56], m, L[7]);
+      L[8] = m2l_fma(D[57], m, L[8]);
+    }
+    { const T m = __ldg(Mr + 21) * rp;
+      L[1] = m2l_fma(D[37], m, L[1]);
+      L[2] = m2l_fma(D[40], m, L[2]);
+      L[3] = m2l_fma(D[41], m, L[3]);
+      L[4] = m2l_fma(D[52], m, L[4]);
+      L[5] = m2l_fma(D[55], m, L[5]);
+      L[6] = m2l_fma(D[56], m, L[6]);
+      L[7] = m2l_fma(D[58], m, L[7]);
+      L[8] = m2l_fma(D[59], m, L[8]);
+    }
+    { const T m = __ldg(Mr + 22) * rp;
+      L[1] = m2l_fma(D[38], m, L[1]);
+      L[2] = m2l_fma(D[41], m, L[2]);
+      L[3] = m2l_fma(D[42], m, L[3]);
+      L[4] = m2l_fma(D[53], m, L[4]);
+      L[5] = m2l_fma(D[56], m, L[5]);
+      L[6] = m2l_fma(D[57], m, L[6]);
+      L[7] = m2l_fma(D[59], m, L[7]);
+      L[8] = m2l_fma(D[60], m, L[8]);
+    }
+    { const T m = __ldg(Mr + 23) * rp;
+      L[1] = m2l_fma(D[40], m, L[1]);
+      L[2] = m2l_fma(D[43], m, L[2]);
+      L[3] = m2l_fma(D[44], m, L[3]);
+      L[4] = m2l_fma(D[55], m, L[4]);
+      L[5] = m2l_fma(D[58], m, L[5]);
+      L[6] = m2l_fma(D[59], m, L[6]);
+      L[7] = m2l_fma(D[61], m, L[7]);
+      L[8] = m2l_fma(D[62], m, L[8]);
+    }
+    { const T m = __ldg(Mr + 24) * rp;
+      L[1] = m2l_fma(D[41], m, L[1]);
+      L[2] = m2l_fma(D[44], m, L[2]);
+      L[3] = m2l_fma(D[45], m, L[3]);
+      L[4] = m2l_fma(D[56], m, L[4]);
+      L[5] = m2l_fma(D[59], m, L[5]);
+      L[6] = m2l_fma(D[60], m, L[6]);
+      L[7] = m2l_fma(D[62], m, L[7]);
+      L[8] = m2l_fma(D[63], m, L[8]);
+    }
+    rp *= rho;
+    { const T m = -__ldg(Mr + 25) * rp;
+      L[1] = m2l_fma(D[46], m, L[1]);
+      L[2] = m2l_fma(D[47], m, L[2]);
+      L[3] = m2l_fma(D[48], m, L[3]);
+    }
+    { const T m = -__ldg(Mr + 26) * rp;
+      L[1] = m2l_fma(D[47], m, L[1]);
+      L[2] = m2l_fma(D[49], m, L[2]);
+      L[3] = m2l_fma(D[50], m, L[3]);
+    }
+    { const T m = -__ldg(Mr + 27) * rp;
+      L[1] = m2l_fma(D[48], m, L[1]);
+      L[2] = m2l_fma(D[50], m, L[2]);
+      L[3] = m2l_fma(D[51], m, L[3]);
+    }
+    { const T m = -__ldg(Mr + 28) * rp;
+      L[1] = m2l_fma(D[49], m, L[1]);
+      L[2] = m2l_fma(D[52], m, L[2]);
+      L[3] = m2l_fma(D[53], m, L[3]);
+    }
+    { const T m = -__ldg(Mr + 29) * rp;
+      L[1] = m2l_fma(D[50], m, L[1]);
+      L[2] = m2l_fma(D[53], m, L[2]);
+      L[3] = m2l_fma(D[54], m, L[3]);
+    }
+    { const T m = -__ldg(Mr + 30) * rp;
+      L[1] = m2l_fma(D[52], m, L[1]);
+      L[2] = m2l_fma(D[55], m, L[2]);
+      L[3] = m2l_fma(D[56], m, L[3]);
+    }
+    { const T m = -__ldg(Mr + 31) * rp;
+      L[1] = m2l_fma(D[53], m, L[1]);
+      L[2] = m2l_fma(D[56], m, L[2]);
+      L[3] = m2l_fma(D[57], m, L[3]);
+    }
+    { const T m = -__ldg(Mr + 32) * rp;
+      L[1] = m2l_fma(D[55], m, L[1]);
+      L[2] = m2l_fma(D[58], m, L[2]);
+      L[3] = m2l_fma(D[59], m, L[3]);
+    }
+    { const T m = -__ldg(Mr + 33) * rp;
+      L[1] = m2l_fma(D[56], m, L[1]);
+      L[2] = m2l_fma(D[59], m, L[2]);
+      L[3] = m2l_fma(D[60], m, L[3]);
+    }
+    { const T m = -__ldg(Mr + 34) * rp;
+      L[1] = m2l_fma(D[58], m, L[1]);
+      L[2] = m2l_fma(D[61], m, L[2]);
+      L[3] = m2l_fma(D[62], m, L[3]);
+    }
+    { const T m = -__ldg(Mr + 35) * rp;
+      L[1] = m2l_fma(D[59], m, L[1]);
+      L[2] = m2l_fma(D[62], m, L[2]);
+      L[3] = m2l_fma(D[63], m, L[3]);
     }
 }
 
-__device__ __forceinline__ void m2l_side_b_h_forces_6(const float (&D)[64], const float *__restrict__ Mr, float (&L)[49])
+template <class T> __device__ __forceinline__ void m2l_side_b_h_forces_6(const T (&D)[64], const T *__restrict__ Mr, T (&L)[49])
 {
-    L[0] = 0.0f;
-    { const float m = __ldg(Mr + 0);
+    L[0] = T(0);
+    { const T m = __ldg(Mr + 0);
       L[1] = -D[1] * m;
       L[2] = -D[2] * m;
       L[3] = -D[3] * m;
@@ -17020,599 +17019,599 @@ __device__ __forceinline__ void m2l_side_b_h_forces_6(const float (&D)[64], cons
       L[47] = D[61] * m;
       L[48] = D[62] * m;
     }
-    { const float m = __ldg(Mr + 1);
-      L[1] = fmaf(-D[4], m, L[1]);
-      L[2] = fmaf(-D[5], m, L[2]);
-      L[3] = fmaf(-D[6], m, L[3]);
-      L[4] = fmaf(D[10], m, L[4]);
-      L[5] = fmaf(D[11], m, L[5]);
-      L[6] = fmaf(D[12], m, L[6]);
-      L[7] = fmaf(D[13], m, L[7]);
-      L[8] = fmaf(D[14], m, L[8]);
-      L[9] = fmaf(-D[19], m, L[9]);
-      L[10] = fmaf(-D[20], m, L[10]);
-      L[11] = fmaf(-D[21], m, L[11]);
-      L[12] = fmaf(-D[22], m, L[12]);
-      L[13] = fmaf(-D[23], m, L[13]);
-      L[14] = fmaf(-D[25], m, L[14]);
-      L[15] = fmaf(-D[26], m, L[15]);
-      L[16] = fmaf(D[31], m, L[16]);
-      L[17] = fmaf(D[32], m, L[17]);
-      L[18] = fmaf(D[33], m, L[18]);
-      L[19] = fmaf(D[34], m, L[19]);
-      L[20] = fmaf(D[35], m, L[20]);
-      L[21] = fmaf(D[37], m, L[21]);
-      L[22] = fmaf(D[38], m, L[22]);
-      L[23] = fmaf(D[40], m, L[23]);
-      L[24] = fmaf(D[41], m, L[24]);
-      L[25] = fmaf(-D[46], m, L[25]);
-      L[26] = fmaf(-D[47], m, L[26]);
-      L[27] = fmaf(-D[48], m, L[27]);
-      L[28] = fmaf(-D[49], m, L[28]);
-      L[29] = fmaf(-D[50], m, L[29]);
-      L[30] = fmaf(-D[52], m, L[30]);
-      L[31] = fmaf(-D[53], m, L[31]);
-      L[32] = fmaf(-D[55], m, L[32]);
-      L[33] = fmaf(-D[56], m, L[33]);
-      L[34] = fmaf(-D[58], m, L[34]);
-      L[35] = fmaf(-D[59], m, L[35]);
+    { const T m = __ldg(Mr + 1);
+      L[1] = m2l_fma(-D[4], m, L[1]);
+      L[2] = m2l_fma(-D[5], m, L[2]);
+      L[3] = m2l_fma(-D[6], m, L[3]);
+      L[4] = m2l_fma(D[10], m, L[4]);
+      L[5] = m2l_fma(D[11], m, L[5]);
+      L[6] = m2l_fma(D[12], m, L[6]);
+      L[7] = m2l_fma(D[13], m, L[7]);
+      L[8] = m2l_fma(D[14], m, L[8]);
+      L[9] = m2l_fma(-D[19], m, L[9]);
+      L[10] = m2l_fma(-D[20], m, L[10]);
+      L[11] = m2l_fma(-D[21], m, L[11]);
+      L[12] = m2l_fma(-D[22], m, L[12]);
+      L[13] = m2l_fma(-D[23], m, L[13]);
+      L[14] = m2l_fma(-D[25], m, L[14]);
+      L[15] = m2l_fma(-D[26], m, L[15]);
+      L[16] = m2l_fma(D[31], m, L[16]);
+      L[17] = m2l_fma(D[32], m, L[17]);
+      L[18] = m2l_fma(D[33], m, L[18]);
+      L[19] = m2l_fma(D[34], m, L[19]);
+      L[20] = m2l_fma(D[35], m, L[20]);
+      L[21] = m2l_fma(D[37], m, L[21]);
+      L[22] = m2l_fma(D[38], m, L[22]);
+      L[23] = m2l_fma(D[40], m, L[23]);
+      L[24] = m2l_fma(D[41], m, L[24]);
+      L[25] = m2l_fma(-D[46], m, L[25]);
+      L[26] = m2l_fma(-D[47], m, L[26]);
+      L[27] = m2l_fma(-D[48], m, L[27]);
+      L[28] = m2l_fma(-D[49], m, L[28]);
+      L[29] = m2l_fma(-D[50], m, L[29]);
+      L[30] = m2l_fma(-D[52], m, L[30]);
+      L[31] = m2l_fma(-D[53], m, L[31]);
+      L[32] = m2l_fma(-D[55], m, L[32]);
+      L[33] = m2l_fma(-D[56], m, L[33]);
+      L[34] = m2l_fma(-D[58], m, L[34]);
+      L[35] = m2l_fma(-D[59], m, L[35]);
     }
-    { const float m = __ldg(Mr + 2);
-      L[1] = fmaf(-D[5], m, L[1]);
-      L[2] = fmaf(-D[7], m, L[2]);
-      L[3] = fmaf(-D[8], m, L[3]);
-      L[4] = fmaf(D[11], m, L[4]);
-      L[5] = fmaf(D[13], m, L[5]);
-      L[6] = fmaf(D[14], m, L[6]);
-      L[7] = fmaf(D[16], m, L[7]);
-      L[8] = fmaf(D[17], m, L[8]);
-      L[9] = fmaf(-D[20], m, L[9]);
-      L[10] = fmaf(-D[22], m, L[10]);
-      L[11] = fmaf(-D[23], m, L[11]);
-      L[12] = fmaf(-D[25], m, L[12]);
-      L[13] = fmaf(-D[26], m, L[13]);
-      L[14] = fmaf(-D[28], m, L[14]);
-      L[15] = fmaf(-D[29], m, L[15]);
-      L[16] = fmaf(D[32], m, L[16]);
-      L[17] = fmaf(D[34], m, L[17]);
-      L[18] = fmaf(D[35], m, L[18]);
-      L[19] = fmaf(D[37], m, L[19]);
-      L[20] = fmaf(D[38], m, L[20]);
-      L[21] = fmaf(D[40], m, L[21]);
-      L[22] = fmaf(D[41], m, L[22]);
-      L[23] = fmaf(D[43], m, L[23]);
-      L[24] = fmaf(D[44], m, L[24]);
-      L[25] = fmaf(-D[47], m, L[25]);
-      L[26] = fmaf(-D[49], m, L[26]);
-      L[27] = fmaf(-D[50], m, L[27]);
-      L[28] = fmaf(-D[52], m, L[28]);
-      L[29] = fmaf(-D[53], m, L[29]);
-      L[30] = fmaf(-D[55], m, L[30]);
-      L[31] = fmaf(-D[56], m, L[31]);
-      L[32] = fmaf(-D[58], m, L[32]);
-      L[33] = fmaf(-D[59], m, L[33]);
-      L[34] = fmaf(-D[61], m, L[34]);
-      L[35] = fmaf(-D[62], m, L[35]);
+    { const T m = __ldg(Mr + 2);
+      L[1] = m2l_fma(-D[5], m, L[1]);
+      L[2] = m2l_fma(-D[7], m, L[2]);
+      L[3] = m2l_fma(-D[8], m, L[3]);
+      L[4] = m2l_fma(D[11], m, L[4]);
+      L[5] = m2l_fma(D[13], m, L[5]);
+      L[6] = m2l_fma(D[14], m, L[6]);
+      L[7] = m2l_fma(D[16], m, L[7]);
+      L[8] = m2l_fma(D[17], m, L[8]);
+      L[9] = m2l_fma(-D[20], m, L[9]);
+      L[10] = m2l_fma(-D[22], m, L[10]);
+      L[11] = m2l_fma(-D[23], m, L[11]);
+      L[12] = m2l_fma(-D[25], m, L[12]);
+      L[13] = m2l_fma(-D[26], m, L[13]);
+      L[14] = m2l_fma(-D[28], m, L[14]);
+      L[15] = m2l_fma(-D[29], m, L[15]);
+      L[16] = m2l_fma(D[32], m, L[16]);
+      L[17] = m2l_fma(D[34], m, L[17]);
+      L[18] = m2l_fma(D[35], m, L[18]);
+      L[19] = m2l_fma(D[37], m, L[19]);
+      L[20] = m2l_fma(D[38], m, L[20]);
+      L[21] = m2l_fma(D[40], m, L[21]);
+      L[22] = m2l_fma(D[41], m, L[22]);
+      L[23] = m2l_fma(D[43], m, L[23]);
+      L[24] = m2l_fma(D[44], m, L[24]);
+      L[25] = m2l_fma(-D[47], m, L[25]);
+      L[26] = m2l_fma(-D[49], m, L[26]);
+      L[27] = m2l_fma(-D[50], m, L[27]);
+      L[28] = m2l_fma(-D[52], m, L[28]);
+      L[29] = m2l_fma(-D[53], m, L[29]);
+      L[30] = m2l_fma(-D[55], m, L[30]);
+      L[31] = m2l_fma(-D[56], m, L[31]);
+      L[32] = m2l_fma(-D[58], m, L[32]);
+      L[33] = m2l_fma(-D[59], m, L[33]);
+      L[34] = m2l_fma(-D[61], m, L[34]);
+      L[35] = m2l_fma(-D[62], m, L[35]);
     }
-    { const float m = __ldg(Mr + 3);
-      L[1] = fmaf(-D[6], m, L[1]);
-      L[2] = fmaf(-D[8], m, L[2]);
-      L[3] = fmaf(-D[9], m, L[3]);
-      L[4] = fmaf(D[12], m, L[4]);
-      L[5] = fmaf(D[14], m, L[5]);
-      L[6] = fmaf(D[15], m, L[6]);
-      L[7] = fmaf(D[17], m, L[7]);
-      L[8] = fmaf(D[18], m, L[8]);
-      L[9] = fmaf(-D[21], m, L[9]);
-      L[10] = fmaf(-D[23], m, L[10]);
-      L[11] = fmaf(-D[24], m, L[11]);
-      L[12] = fmaf(-D[26], m, L[12]);
-      L[13] = fmaf(-D[27], m, L[13]);
-      L[14] = fmaf(-D[29], m, L[14]);
-      L[15] = fmaf(-D[30], m, L[15]);
-      L[16] = fmaf(D[33], m, L[16]);
-      L[17] = fmaf(D[35], m, L[17]);
-      L[18] = fmaf(D[36], m, L[18]);
-      L[19] = fmaf(D[38], m, L[19]);
-      L[20] = fmaf(D[39], m, L[20]);
-      L[21] = fmaf(D[41], m, L[21]);
-      L[22] = fmaf(D[42], m, L[22]);
-      L[23] = fmaf(D[44], m, L[23]);
-      L[24] = fmaf(D[45], m, L[24]);
-      L[25] = fmaf(-D[48], m, L[25]);
-      L[26] = fmaf(-D[50], m, L[26]);
-      L[27] = fmaf(-D[51], m, L[27]);
-      L[28] = fmaf(-D[53], m, L[28]);
-      L[29] = fmaf(-D[54], m, L[29]);
-      L[30] = fmaf(-D[56], m, L[30]);
-      L[31] = fmaf(-D[57], m, L[31]);
-      L[32] = fmaf(-D[59], m, L[32]);
-      L[33] = fmaf(-D[60], m, L[33]);
-      L[34] = fmaf(-D[62], m, L[34]);
-      L[35] = fmaf(-D[63], m, L[35]);
+    { const T m = __ldg(Mr + 3);
+      L[1] = m2l_fma(-D[6], m, L[1]);
+      L[2] = m2l_fma(-D[8], m, L[2]);
+      L[3] = m2l_fma(-D[9], m, L[3]);
+      L[4] = m2l_fma(D[12], m, L[4]);
+      L[5] = m2l_fma(D[14], m, L[5]);
+      L[6] = m2l_fma(D[15], m, L[6]);
+      L[7] = m2l_fma(D[17], m, L[7]);
+      L[8] = m2l_fma(D[18], m, L[8]);
+      L[9] = m2l_fma(-D[21], m, L[9]);
+      L[10] = m2l_fma(-D[23], m, L[10]);
+      L[11] = m2l_fma(-D[24], m, L[11]);
+      L[12] = m2l_fma(-D[26], m, L[12]);
+      L[13] = m2l_fma(-D[27], m, L[13]);
+      L[14] = m2l_fma(-D[29], m, L[14]);
+      L[15] = m2l_fma(-D[30], m, L[15]);
+      L[16] = m2l_fma(D[33], m, L[16]);
+      L[17] = m2l_fma(D[35], m, L[17]);
+      L[18] = m2l_fma(D[36], m, L[18]);
+      L[19] = m2l_fma(D[38], m, L[19]);
+      L[20] = m2l_fma(D[39], m, L[20]);
+      L[21] = m2l_fma(D[41], m, L[21]);
+      L[22] = m2l_fma(D[42], m, L[22]);
+      L[23] = m2l_fma(D[44], m, L[23]);
+      L[24] = m2l_fma(D[45], m, L[24]);
+      L[25] = m2l_fma(-D[48], m, L[25]);
+      L[26] = m2l_fma(-D[50], m, L[26]);
+      L[27] = m2l_fma(-D[51], m, L[27]);
+      L[28] = m2l_fma(-D[53], m, L[28]);
+      L[29] = m2l_fma(-D[54], m, L[29]);
+      L[30] = m2l_fma(-D[56], m, L[30]);
+      L[31] = m2l_fma(-D[57], m, L[31]);
+      L[32] = m2l_fma(-D[59], m, L[32]);
+      L[33] = m2l_fma(-D[60], m, L[33]);
+      L[34] = m2l_fma(-D[62], m, L[34]);
+      L[35] = m2l_fma(-D[63], m, L[35]);
     }
-    { const float m = __ldg(Mr + 4);
-      L[1] = fmaf(-D[10], m, L[1]);
-      L[2] = fmaf(-D[11], m, L[2]);
-      L[3] = fmaf(-D[12], m, L[3]);
-      L[4] = fmaf(D[19], m, L[4]);
-      L[5] = fmaf(D[20], m, L[5]);
-      L[6] = fmaf(D[21], m, L[6]);
-      L[7] = fmaf(D[22], m, L[7]);
-      L[8] = fmaf(D[23], m, L[8]);
-      L[9] = fmaf(-D[31], m, L[9]);
-      L[10] = fmaf(-D[32], m, L[10]);
-      L[11] = fmaf(-D[33], m, L[11]);
-      L[12] = fmaf(-D[34], m, L[12]);
-      L[13] = fmaf(-D[35], m, L[13]);
-      L[14] = fmaf(-D[37], m, L[14]);
-      L[15] = fmaf(-D[38], m, L[15]);
-      L[16] = fmaf(D[46], m, L[16]);
-      L[17] = fmaf(D[47], m, L[17]);
-      L[18] = fmaf(D[48], m, L[18]);
-      L[19] = fmaf(D[49], m, L[19]);
-      L[20] = fmaf(D[50], m, L[20]);
-      L[21] = fmaf(D[52], m, L[21]);
-      L[22] = fmaf(D[53], m, L[22]);
-      L[23] = fmaf(D[55], m, L[23]);
-      L[24] = fmaf(D[56], m, L[24]);
+    { const T m = __ldg(Mr + 4);
+      L[1] = m2l_fma(-D[10], m, L[1]);
+      L[2] = m2l_fma(-D[11], m, L[2]);
+      L[3] = m2l_fma(-D[12], m, L[3]);
+      L[4] = m2l_fma(D[19], m, L[4]);
+      L[5] = m2l_fma(D[20], m, L[5]);
+      L[6] = m2l_fma(D[21], m, L[6]);
+      L[7] = m2l_fma(D[22], m, L[7]);
+      L[8] = m2l_fma(D[23], m, L[8]);
+      L[9] = m2l_fma(-D[31], m, L[9]);
+      L[10] = m2l_fma(-D[32], m, L[10]);
+      L[11] = m2l_fma(-D[33], m, L[11]);
+      L[12] = m2l_fma(-D[34], m, L[12]);
+      L[13] = m2l_fma(-D[35], m, L[13]);
+      L[14] = m2l_fma(-D[37], m, L[14]);
+      L[15] = m2l_fma(-D[38], m, L[15]);
+      L[16] = m2l_fma(D[46], m, L[16]);
+      L[17] = m2l_fma(D[47], m, L[17]);
+      L[18] = m2l_fma(D[48], m, L[18]);
+      L[19] = m2l_fma(D[49], m, L[19]);
+      L[20] = m2l_fma(D[50], m, L[20]);
+      L[21] = m2l_fma(D[52], m, L[21]);
+      L[22] = m2l_fma(D[53], m, L[22]);
+      L[23] = m2l_fma(D[55], m, L[23]);
+      L[24] = m2l_fma(D[56], m, L[24]);
     }
-    { const float m = __ldg(Mr + 5);
-      L[1] = fmaf(-D[11], m, L[1]);
-      L[2] = fmaf(-D[13], m, L[2]);
-      L[3] = fmaf(-D[14], m, L[3]);
-      L[4] = fmaf(D[20], m, L[4]);
-      L[5] = fmaf(D[22], m, L[5]);
-      L[6] = fmaf(D[23], m, L[6]);
-      L[7] = fmaf(D[25], m, L[7]);
-      L[8] = fmaf(D[26], m, L[8]);
-      L[9] = fmaf(-D[32], m, L[9]);
-      L[10] = fmaf(-D[34], m, L[10]);
-      L[11] = fmaf(-D[35], m, L[11]);
-      L[12] = fmaf(-D[37], m, L[12]);
-      L[13] = fmaf(-D[38], m, L[13]);
-      L[14] = fmaf(-D[40], m, L[14]);
-      L[15] = fmaf(-D[41], m, L[15]);
-      L[16] = fmaf(D[47], m, L[16]);
-      L[17] = fmaf(D[49], m, L[17]);
-      L[18] = fmaf(D[50], m, L[18]);
-      L[19] = fmaf(D[52], m, L[19]);
-      L[20] = fmaf(D[53], m, L[20]);
-      L[21] = fmaf(D[55], m, L[21]);
-      L[22] = fmaf(D[56], m, L[22]);
-      L[23] = fmaf(D[58], m, L[23]);
-      L[24] = fmaf(D[59], m, L[24]);
+    { const T m = __ldg(Mr + 5);
+      L[1] = m2l_fma(-D[11], m, L[1]);
+      L[2] = m2l_fma(-D[13], m, L[2]);
+      L[3] = m2l_fma(-D[14], m, L[3]);
+      L[4] = m2l_fma(D[20], m, L[4]);
+      L[5] = m2l_fma(D[22], m, L[5]);
+      L[6] = m2l_fma(D[23], m, L[6]);
+      L[7] = m2l_fma(D[25], m, L[7]);
+      L[8] = m2l_fma(D[26], m, L[8]);
+      L[9] = m2l_fma(-D[32], m, L[9]);
+      L[10] = m2l_fma(-D[34], m, L[10]);
+      L[11] = m2l_fma(-D[35], m, L[11]);
+      L[12] = m2l_fma(-D[37], m, L[12]);
+      L[13] = m2l_fma(-D[38], m, L[13]);
+      L[14] = m2l_fma(-D[40], m, L[14]);
+      L[15] = m2l_fma(-D[41], m, L[15]);
+      L[16] = m2l_fma(D[47], m, L[16]);
+      L[17] = m2l_fma(D[49], m, L[17]);
+      L[18] = m2l_fma(D[50], m, L[18]);
+      L[19] = m2l_fma(D[52], m, L[19]);
+      L[20] = m2l_fma(D[53], m, L[20]);
+      L[21] = m2l_fma(D[55], m, L[21]);
+      L[22] = m2l_fma(D[56], m, L[22]);
+      L[23] = m2l_fma(D[58], m, L[23]);
+      L[24] = m2l_fma(D[59], m, L[24]);
     }
-    { const float m = __ldg(Mr + 6);
-      L[1] = fmaf(-D[12], m, L[1]);
-      L[2] = fmaf(-D[14], m, L[2]);
-      L[3] = fmaf(-D[15], m, L[3]);
-      L[4] = fmaf(D[21], m, L[4]);
-      L[5] = fmaf(D[23], m, L[5]);
-      L[6] = fmaf(D[24], m, L[6]);
-      L[7] = fmaf(D[26], m, L[7]);
-      L[8] = fmaf(D[27], m, L[8]);
-      L[9] = fmaf(-D[33], m, L[9]);
-      L[10] = fmaf(-D[35], m, L[10]);
-      L[11] = fmaf(-D[36], m, L[11]);
-      L[12] = fmaf(-D[38], m, L[12]);
-      L[13] = fmaf(-D[39], m, L[13]);
-      L[14] = fmaf(-D[41], m, L[14]);
-      L[15] = fmaf(-D[42], m, L[15]);
-      L[16] = fmaf(D[48], m, L[16]);
-      L[17] = fmaf(D[50], m, L[17]);
-      L[18] = fmaf(D[51], m, L[18]);
-      L[19] = fmaf(D[53], m, L[19]);
-      L[20] = fmaf(D[54], m, L[20]);
-      L[21] = fmaf(D[56], m, L[21]);
-      L[22] = fmaf(D[57], m, L[22]);
-      L[23] = fmaf(D[59], m, L[23]);
-      L[24] = fmaf(D[60], m, L[24]);
+    { const T m = __ldg(Mr + 6);
+      L[1] = m2l_fma(-D[12], m, L[1]);
+      L[2] = m2l_fma(-D[14], m, L[2]);
+      L[3] = m2l_fma(-D[15], m, L[3]);
+      L[4] = m2l_fma(D[21], m, L[4]);
+      L[5] = m2l_fma(D[23], m, L[5]);
+      L[6] = m2l_fma(D[24], m, L[6]);
+      L[7] = m2l_fma(D[26], m, L[7]);
+      L[8] = m2l_fma(D[27], m, L[8]);
+      L[9] = m2l_fma(-D[33], m, L[9]);
+      L[10] = m2l_fma(-D[35], m, L[10]);
+      L[11] = m2l_fma(-D[36], m, L[11]);
+      L[12] = m2l_fma(-D[38], m, L[12]);
+      L[13] = m2l_fma(-D[39], m, L[13]);
+      L[14] = m2l_fma(-D[41], m, L[14]);
+      L[15] = m2l_fma(-D[42], m, L[15]);
+      L[16] = m2l_fma(D[48], m, L[16]);
+      L[17] = m2l_fma(D[50], m, L[17]);
+      L[18] = m2l_fma(D[51], m, L[18]);
+      L[19] = m2l_fma(D[53], m, L[19]);
+      L[20] = m2l_fma(D[54], m, L[20]);
+      L[21] = m2l_fma(D[56], m, L[21]);
+      L[22] = m2l_fma(D[57], m, L[22]);
+      L[23] = m2l_fma(D[59], m, L[23]);
+      L[24] = m2l_fma(D[60], m, L[24]);
     }
-    { const float m = __ldg(Mr + 7);
-      L[1] = fmaf(-D[13], m, L[1]);
-      L[2] = fmaf(-D[16], m, L[2]);
-      L[3] = fmaf(-D[17], m, L[3]);
-      L[4] = fmaf(D[22], m, L[4]);
-      L[5] = fmaf(D[25], m, L[5]);
-      L[6] = fmaf(D[26], m, L[6]);
-      L[7] = fmaf(D[28], m, L[7]);
-      L[8] = fmaf(D[29], m, L[8]);
-      L[9] = fmaf(-D[34], m, L[9]);
-      L[10] = fmaf(-D[37], m, L[10]);
-      L[11] = fmaf(-D[38], m, L[11]);
-      L[12] = fmaf(-D[40], m, L[12]);
-      L[13] = fmaf(-D[41], m, L[13]);
-      L[14] = fmaf(-D[43], m, L[14]);
-      L[15] = fmaf(-D[44], m, L[15]);
-      L[16] = fmaf(D[49], m, L[16]);
-      L[17] = fmaf(D[52], m, L[17]);
-      L[18] = fmaf(D[53], m, L[18]);
-      L[19] = fmaf(D[55], m, L[19]);
-      L[20] = fmaf(D[56], m, L[20]);
-      L[21] = fmaf(D[58], m, L[21]);
-      L[22] = fmaf(D[59], m, L[22]);
-      L[23] = fmaf(D[61], m, L[23]);
-      L[24] = fmaf(D[62], m, L[24]);
+    { const T m = __ldg(Mr + 7);
+      L[1] = m2l_fma(-D[13], m, L[1]);
+      L[2] = m2l_fma(-D[16], m, L[2]);
+      L[3] = m2l_fma(-D[17], m, L[3]);
+      L[4] = m2l_fma(D[22], m, L[4]);
+      L[5] = m2l_fma(D[25], m, L[5]);
+      L[6] = m2l_fma(D[26], m, L[6]);
+      L[7] = m2l_fma(D[28], m, L[7]);
+      L[8] = m2l_fma(D[29], m, L[8]);
+      L[9] = m2l_fma(-D[34], m, L[9]);
+      L[10] = m2l_fma(-D[37], m, L[10]);
+      L[11] = m2l_fma(-D[38], m, L[11]);
+      L[12] = m2l_fma(-D[40], m, L[12]);
+      L[13] = m2l_fma(-D[41], m, L[13]);
+      L[14] = m2l_fma(-D[43], m, L[14]);
+      L[15] = m2l_fma(-D[44], m, L[15]);
+      L[16] = m2l_fma(D[49], m, L[16]);
+      L[17] = m2l_fma(D[52], m, L[17]);
+      L[18] = m2l_fma(D[53], m, L[18]);
+      L[19] = m2l_fma(D[55], m, L[19]);
+      L[20] = m2l_fma(D[56], m, L[20]);
+      L[21] = m2l_fma(D[58], m, L[21]);
+      L[22] = m2l_fma(D[59], m, L[22]);
+      L[23] = m2l_fma(D[61], m, L[23]);
+      L[24] = m2l_fma(D[62], m, L[24]);
     }
-    { const float m = __ldg(Mr + 8);
-      L[1] = fmaf(-D[14], m, L[1]);
-      L[2] = fmaf(-D[17], m, L[2]);
-      L[3] = fmaf(-D[18], m, L[3]);
-      L[4] = fmaf(D[23], m, L[4]);
-      L[5] = fmaf(D[26], m, L[5]);
-      L[6] = fmaf(D[27], m, L[6]);
-      L[7] = fmaf(D[29], m, L[7]);
-      L[8] = fmaf(D[30], m, L[8]);
-      L[9] = fmaf(-D[35], m, L[9]);
-      L[10] = fmaf(-D[38], m, L[10]);
-      L[11] = fmaf(-D[39], m, L[11]);
-      L[12] = fmaf(-D[41], m, L[12]);
-      L[13] = fmaf(-D[42], m, L[13]);
-      L[14] = fmaf(-D[44], m, L[14]);
-      L[15] = fmaf(-D[45], m, L[15]);
-      L[16] = fmaf(D[50], m, L[16]);
-      L[17] = fmaf(D[53], m, L[17]);
-      L[18] = fmaf(D[54], m, L[18]);
-      L[19] = fmaf(D[56], m, L[19]);
-      L[20] = fmaf(D[57], m, L[20]);
-      L[21] = fmaf(D[59], m, L[21]);
-      L[22] = fmaf(D[60], m, L[22]);
-      L[23] = fmaf(D[62], m, L[23]);
-      L[24] = fmaf(D[63], m, L[24]);
+    { const T m = __ldg(Mr + 8);
+      L[1] = m2l_fma(-D[14], m, L[1]);
+      L[2] = m2l_fma(-D[17], m, L[2]);
+      L[3] = m2l_fma(-D[18], m, L[3]);
+      L[4] = m2l_fma(D[23], m, L[4]);
+      L[5] = m2l_fma(D[26], m, L[5]);
+      L[6] = m2l_fma(D[27], m, L[6]);
+      L[7] = m2l_fma(D[29], m, L[7]);
+      L[8] = m2l_fma(D[30], m, L[8]);
+      L[9] = m2l_fma(-D[35], m, L[9]);
+      L[10] = m2l_fma(-D[38], m, L[10]);
+      L[11] = m2l_fma(-D[39], m, L[11]);
+      L[12] = m2l_fma(-D[41], m, L[12]);
+      L[13] = m2l_fma(-D[42], m, L[13]);
+      L[14] = m2l_fma(-D[44], m, L[14]);
+      L[15] = m2l_fma(-D[45], m, L[15]);
+      L[16] = m2l_fma(D[50], m, L[16]);
+      L[17] = m2l_fma(D[53], m, L[17]);
+      L[18] = m2l_fma(D[54], m, L[18]);
+      L[19] = m2l_fma(D[56], m, L[19]);
+      L[20] = m2l_fma(D[57], m, L[20]);
+      L[21] = m2l_fma(D[59], m, L[21]);
+      L[22] = m2l_fma(D[60], m, L[22]);
+      L[23] = m2l_fma(D[62], m, L[23]);
+      L[24] = m2l_fma(D[63], m, L[24]);
     }
-    { const float m = __ldg(Mr + 9);
-      L[1] = fmaf(-D[19], m, L[1]);
-      L[2] = fmaf(-D[20], m, L[2]);
-      L[3] = fmaf(-D[21], m, L[3]);
-      L[4] = fmaf(D[31], m, L[4]);
-      L[5] = fmaf(D[32], m, L[5]);
-      L[6] = fmaf(D[33], m, L[6]);
-      L[7] = fmaf(D[34], m, L[7]);
-      L[8] = fmaf(D[35], m, L[8]);
-      L[9] = fmaf(-D[46], m, L[9]);
-      L[10] = fmaf(-D[47], m, L[10]);
-      L[11] = fmaf(-D[48], m, L[11]);
-      L[12] = fmaf(-D[49], m, L[12]);
-      L[13] = fmaf(-D[50], m, L[13]);
-      L[14] = fmaf(-D[52], m, L[14]);
-      L[15] = fmaf(-D[53], m, L[15]);
+    { const T m = __ldg(Mr + 9);
+      L[1] = m2l_fma(-D[19], m, L[1]);
+      L[2] = m2l_fma(-D[20], m, L[2]);
+      L[3] = m2l_fma(-D[21], m, L[3]);
+      L[4] = m2l_fma(D[31], m, L[4]);
+      L[5] = m2l_fma(D[32], m, L[5]);
+      L[6] = m2l_fma(D[33], m, L[6]);
+      L[7] = m2l_fma(D[34], m, L[7]);
+      L[8] = m2l_fma(D[35], m, L[8]);
+      L[9] = m2l_fma(-D[46], m, L[9]);
+      L[10] = m2l_fma(-D[47], m, L[10]);
+      L[11] = m2l_fma(-D[48], m, L[11]);
+      L[12] = m2l_fma(-D[49], m, L[12]);
+      L[13] = m2l_fma(-D[50], m, L[13]);
+      L[14] = m2l_fma(-D[52], m, L[14]);
+      L[15] = m2l_fma(-D[53], m, L[15]);
     }
-    { const float m = __ldg(Mr + 10);
-      L[1] = fmaf(-D[20], m, L[1]);
-      L[2] = fmaf(-D[22], m, L[2]);
-      L[3] = fmaf(-D[23], m, L[3]);
-      L[4] = fmaf(D[32], m, L[4]);
-      L[5] = fmaf(D[34], m, L[5]);
-      L[6] = fmaf(D[35], m, L[6]);
-      L[7] = fmaf(D[37], m, L[7]);
-      L[8] = fmaf(D[38], m, L[8]);
-      L[9] = fmaf(-D[47], m, L[9]);
-      L[10] = fmaf(-D[49], m, L[10]);
-      L[11] = fmaf(-D[50], m, L[11]);
-      L[12] = fmaf(-D[52], m, L[12]);
-      L[13] = fmaf(-D[53], m, L[13]);
-      L[14] = fmaf(-D[55], m, L[14]);
-      L[15] = fmaf(-D[56], m, L[15]);
+    { const T m = __ldg(Mr + 10);
+      L[1] = m2l_fma(-D[20], m, L[1]);
+      L[2] = m2l_fma(-D[22], m, L[2]);
+      L[3] = m2l_fma(-D[23], m, L[3]);
+      L[4] = m2l_fma(D[32], m, L[4]);
+      L[5] = m2l_fma(D[34], m, L[5]);
+      L[6] = m2l_fma(D[35], m, L[6]);
+      L[7] = m2l_fma(D[37], m, L[7]);
+      L[8] = m2l_fma(D[38], m, L[8]);
+      L[9] = m2l_fma(-D[47], m, L[9]);
+      L[10] = m2l_fma(-D[49], m, L[10]);
+      L[11] = m2l_fma(-D[50], m, L[11]);
+      L[12] = m2l_fma(-D[52], m, L[12]);
+      L[13] = m2l_fma(-D[53], m, L[13]);
+      L[14] = m2l_fma(-D[55], m, L[14]);
+      L[15] = m2l_fma(-D[56], m, L[15]);
     }
-    { const float m = __ldg(Mr + 11);
-      L[1] = fmaf(-D[21], m, L[1]);
-      L[2] = fmaf(-D[23], m, L[2]);
-      L[3] = fmaf(-D[24], m, L[3]);
-      L[4] = fmaf(D[33], m, L[4]);
-      L[5] = fmaf(D[35], m, L[5]);
-      L[6] = fmaf(D[36], m, L[6]);
-      L[7] = fmaf(D[38], m, L[7]);
-      L[8] = fmaf(D[39], m, L[8]);
-      L[9] = fmaf(-D[48], m, L[9]);
-      L[10] = fmaf(-D[50], m, L[10]);
-      L[11] = fmaf(-D[51], m, L[11]);
-      L[12] = fmaf(-D[53], m, L[12]);
-      L[13] = fmaf(-D[54], m, L[13]);
-      L[14] = fmaf(-D[56], m, L[14]);
-      L[15] = fmaf(-D[57], m, L[15]);
+    { const T m = __ldg(Mr + 11);
+      L[1] = m2l_fma(-D[21], m, L[1]);
+      L[2] = m2l_fma(-D[23], m, L[2]);
+      L[3] = m2l_fma(-D[24], m, L[3]);
+      L[4] = m2l_fma(D[33], m, L[4]);
+      L[5] = m2l_fma(D[35], m, L[5]);
+      L[6] = m2l_fma(D[36], m, L[6]);
+      L[7] = m2l_fma(D[38], m, L[7]);
+      L[8] = m2l_fma(D[39], m, L[8]);
+      L[9] = m2l_fma(-D[48], m, L[9]);
+      L[10] = m2l_fma(-D[50], m, L[10]);
+      L[11] = m2l_fma(-D[51], m, L[11]);
+      L[12] = m2l_fma(-D[53], m, L[12]);
+      L[13] = m2l_fma(-D[54], m, L[13]);
+      L[14] = m2l_fma(-D[56], m, L[14]);
+      L[15] = m2l_fma(-D[57], m, L[15]);
     }
-    { const float m = __ldg(Mr + 12);
-      L[1] = fmaf(-D[22], m, L[1]);
-      L[2] = fmaf(-D[25], m, L[2]);
-      L[3] = fmaf(-D[26], m, L[3]);
-      L[4] = fmaf(D[34], m, L[4]);
-      L[5] = fmaf(D[37], m, L[5]);
-      L[6] = fmaf(D[38], m, L[6]);
-      L[7] = fmaf(D[40], m, L[7]);
-      L[8] = fmaf(D[41], m, L[8]);
-      L[9] = fmaf(-D[49], m, L[9]);
-      L[10] = fmaf(-D[52], m, L[10]);
-      L[11] = fmaf(-D[53], m, L[11]);
-      L[12] = fmaf(-D[55], m, L[12]);
-      L[13] = fmaf(-D[56], m, L[13]);
-      L[14] = fmaf(-D[58], m, L[14]);
-      L[15] = fmaf(-D[59], m, L[15]);
+    { const T m = __ldg(Mr + 12);
+      L[1] = m2l_fma(-D[22], m, L[1]);
+      L[2] = m2l_fma(-D[25], m, L[2]);
+      L[3] = m2l_fma(-D[26], m, L[3]);
+      L[4] = m2l_fma(D[34], m, L[4]);
+      L[5] = m2l_fma(D[37], m, L[5]);
+      L[6] = m2l_fma(D[38], m, L[6]);
+      L[7] = m2l_fma(D[40], m, L[7]);
+      L[8] = m2l_fma(D[41], m, L[8]);
+      L[9] = m2l_fma(-D[49], m, L[9]);
+      L[10] = m2l_fma(-D[52], m, L[10]);
+      L[11] = m2l_fma(-D[53], m, L[11]);
+      L[12] = m2l_fma(-D[55], m, L[12]);
+      L[13] = m2l_fma(-D[56], m, L[13]);
+      L[14] = m2l_fma(-D[58], m, L[14]);
+      L[15] = m2l_fma(-D[59], m, L[15]);
     }
-    { const float m = __ldg(Mr + 13);
-      L[1] = fmaf(-D[23], m, L[1]);
-      L[2] = fmaf(-D[26], m, L[2]);
-      L[3] = fmaf(-D[27], m, L[3]);
-      L[4] = fmaf(D[35], m, L[4]);
-      L[5] = fmaf(D[38], m, L[5]);
-      L[6] = fmaf(D[39], m, L[6]);
-      L[7] = fmaf(D[41], m, L[7]);
-      L[8] = fmaf(D[42], m, L[8]);
-      L[9] = fmaf(-D[50], m, L[9]);
-      L[10] = fmaf(-D[53], m, L[10]);
-      L[11] = fmaf(-D[54], m, L[11]);
-      L[12] = fmaf(-D[56], m, L[12]);
-      L[13] = fmaf(-D[57], m, L[13]);
-      L[14] = fmaf(-D[59], m, L[14]);
-      L[15] = fmaf(-D[60], m, L[15]);
+    { const T m = __ldg(Mr + 13);
+      L[1] = m2l_fma(-D[23], m, L[1]);
+      L[2] = m2l_fma(-D[26], m, L[2]);
+      L[3] = m2l_fma(-D[27], m, L[3]);
+      L[4] = m2l_fma(D[35], m, L[4]);
+      L[5] = m2l_fma(D[38], m, L[5]);
+      L[6] = m2l_fma(D[39], m, L[6]);
+      L[7] = m2l_fma(D[41], m, L[7]);
+      L[8] = m2l_fma(D[42], m, L[8]);
+      L[9] = m2l_fma(-D[50], m, L[9]);
+      L[10] = m2l_fma(-D[53], m, L[10]);
+      L[11] = m2l_fma(-D[54], m, L[11]);
+      L[12] = m2l_fma(-D[56], m, L[12]);
+      L[13] = m2l_fma(-D[57], m, L[13]);
+      L[14] = m2l_fma(-D[59], m, L[14]);
+      L[15] = m2l_fma(-D[60], m, L[15]);
     }
-    { const float m = __ldg(Mr + 14);
-      L[1] = fmaf(-D[25], m, L[1]);
-      L[2] = fmaf(-D[28], m, L[2]);
-      L[3] = fmaf(-D[29], m, L[3]);
-      L[4] = fmaf(D[37], m, L[4]);
-      L[5] = fmaf(D[40], m, L[5]);
-      L[6] = fmaf(D[41], m, L[6]);
-      L[7] = fmaf(D[43], m, L[7]);
-      L[8] = fmaf(D[44], m, L[8]);
-      L[9] = fmaf(-D[52], m, L[9]);
-      L[10] = fmaf(-D[55], m, L[10]);
-      L[11] = fmaf(-D[56], m, L[11]);
-      L[12] = fmaf(-D[58], m, L[12]);
-      L[13] = fmaf(-D[59], m, L[13]);
-      L[14] = fmaf(-D[61], m, L[14]);
-      L[15] = fmaf(-D[62], m, L[15]);
+    { const T m = __ldg(Mr + 14);
+      L[1] = m2l_fma(-D[25], m, L[1]);
+      L[2] = m2l_fma(-D[28], m, L[2]);
+      L[3] = m2l_fma(-D[29], m, L[3]);
+      L[4] = m2l_fma(D[37], m, L[4]);
+      L[5] = m2l_fma(D[40], m, L[5]);
+      L[6] = m2l_fma(D[41], m, L[6]);
+      L[7] = m2l_fma(D[43], m, L[7]);
+      L[8] = m2l_fma(D[44], m, L[8]);
+      L[9] = m2l_fma(-D[52], m, L[9]);
+      L[10] = m2l_fma(-D[55], m, L[10]);
+      L[11] = m2l_fma(-D[56], m, L[11]);
+      L[12] = m2l_fma(-D[58], m, L[12]);
+      L[13] = m2l_fma(-D[59], m, L[13]);
+      L[14] = m2l_fma(-D[61], m, L[14]);
+      L[15] = m2l_fma(-D[62], m, L[15]);
     }
-    { const float m = __ldg(Mr + 15);
-      L[1] = fmaf(-D[26], m, L[1]);
-      L[2] = fmaf(-D[29], m, L[2]);
-      L[3] = fmaf(-D[30], m, L[3]);
-      L[4] = fmaf(D[38], m, L[4]);
-      L[5] = fmaf(D[41], m, L[5]);
-      L[6] = fmaf(D[42], m, L[6]);
-      L[7] = fmaf(D[44], m, L[7]);
-      L[8] = fmaf(D[45], m, L[8]);
-      L[9] = fmaf(-D[53], m, L[9]);
-      L[10] = fmaf(-D[56], m, L[10]);
-      L[11] = fmaf(-D[57], m, L[11]);
-      L[12] = fmaf(-D[59], m, L[12]);
-      L[13] = fmaf(-D[60], m, L[13]);
-      L[14] = fmaf(-D[62], m, L[14]);
-      L[15] = fmaf(-D[63], m, L[15]);
+    { const T m = __ldg(Mr + 15);
+      L[1] = m2l_fma(-D[26], m, L[1]);
+      L[2] = m2l_fma(-D[29], m, L[2]);
+      L[3] = m2l_fma(-D[30], m, L[3]);
+      L[4] = m2l_fma(D[38], m, L[4]);
+      L[5] = m2l_fma(D[41], m, L[5]);
+      L[6] = m2l_fma(D[42], m, L[6]);
+      L[7] = m2l_fma(D[44], m, L[7]);
+      L[8] = m2l_fma(D[45], m, L[8]);
+      L[9] = m2l_fma(-D[53], m, L[9]);
+      L[10] = m2l_fma(-D[56], m, L[10]);
+      L[11] = m2l_fma(-D[57], m, L[11]);
+      L[12] = m2l_fma(-D[59], m, L[12]);
+      L[13] = m2l_fma(-D[60], m, L[13]);
+      L[14] = m2l_fma(-D[62], m, L[14]);
+      L[15] = m2l_fma(-D[63], m, L[15]);
     }
-    { const float m = __ldg(Mr + 16);
-      L[1] = fmaf(-D[31], m, L[1]);
-      L[2] = fmaf(-D[32], m, L[2]);
-      L[3] = fmaf(-D[33], m, L[3]);
-      L[4] = fmaf(D[46], m, L[4]);
-      L[5] = fmaf(D[47], m, L[5]);
-      L[6] = fmaf(D[48], m, L[6]);
-      L[7] = fmaf(D[49], m, L[7]);
-      L[8] = fmaf(D[50], m, L[8]);
+    { const T m = __ldg(Mr + 16);
+      L[1] = m2l_fma(-D[31], m, L[1]);
+      L[2] = m2l_fma(-D[32], m, L[2]);
+      L[3] = m2l_fma(-D[33], m, L[3]);
+      L[4] = m2l_fma(D[46], m, L[4]);
+      L[5] = m2l_fma(D[47], m, L[5]);
+      L[6] = m2l_fma(D[48], m, L[6]);
+      L[7] = m2l_fma(D[49], m, L[7]);
+      L[8] = m2l_fma(D[50], m, L[8]);
     }
-    { const float m = __ldg(Mr + 17);
-      L[1] = fmaf(-D[32], m, L[1]);
-      L[2] = fmaf(-D[34], m, L[2]);
-      L[3] = fmaf(-D[35], m, L[3]);
-      L[4] = fmaf(D[47], m, L[4]);
-      L[5] = fmaf(D[49], m, L[5]);
-      L[6] = fmaf(D[50], m, L[6]);
-      L[7] = fmaf(D[52], m, L[7]);
-      L[8] = fmaf(D[53], m, L[8]);
+    { const T m = __ldg(Mr + 17);
+      L[1] = m2l_fma(-D[32], m, L[1]);
+      L[2] = m2l_fma(-D[34], m, L[2]);
+      L[3] = m2l_fma(-D[35], m, L[3]);
+      L[4] = m2l_fma(D[47], m, L[4]);
+      L[5] = m2l_fma(D[49], m, L[5]);
+      L[6] = m2l_fma(D[50], m, L[6]);
+      L[7] = m2l_fma(D[52], m, L[7]);
+      L[8] = m2l_fma(D[53], m, L[8]);
     }
-    { const float m = __ldg(Mr + 18);
-      L[1] = fmaf(-D[33], m, L[1]);
-      L[2] = fmaf(-D[35], m, L[2]);
-      L[3] = fmaf(-D[36], m, L[3]);
-      L[4] = fmaf(D[48], m, L[4]);
-      L[5] = fmaf(D[50], m, L[5]);
-      L[6] = fmaf(D[51], m, L[6]);
-      L[7] = fmaf(D[53], m, L[7]);
-      L[8] = fmaf(D[54], m, L[8]);
+    { const T m = __ldg(Mr + 18);
+      L[1] = m2l_fma(-D[33], m, L[1]);
+      L[2] = m2l_fma(-D[35], m, L[2]);
+      L[3] = m2l_fma(-D[36], m, L[3]);
+      L[4] = m2l_fma(D[48], m, L[4]);
+      L[5] = m2l_fma(D[50], m, L[5]);
+      L[6] = m2l_fma(D[51], m, L[6]);
+      L[7] = m2l_fma(D[53], m, L[7]);
+      L[8] = m2l_fma(D[54], m, L[8]);
     }
-    { const float m = __ldg(Mr + 19);
-      L[1] = fmaf(-D[34], m, L[1]);
-      L[2] = fmaf(-D[37], m, L[2]);
-      L[3] = fmaf(-D[38], m, L[3]);
-      L[4] = fmaf(D[49], m, L[4]);
-      L[5] = fmaf(D[52], m, L[5]);
-      L[6] = fmaf(D[53], m, L[6]);
-      L[7] = fmaf(D[55], m, L[7]);
-      L[8] = fmaf(D[56], m, L[8]);
+    { const T m = __ldg(Mr + 19);
+      L[1] = m2l_fma(-D[34], m, L[1]);
+      L[2] = m2l_fma(-D[37], m, L[2]);
+      L[3] = m2l_fma(-D[38], m, L[3]);
+      L[4] = m2l_fma(D[49], m, L[4]);
+      L[5] = m2l_fma(D[52], m, L[5]);
+      L[6] = m2l_fma(D[53], m, L[6]);
+      L[7] = m2l_fma(D[55], m, L[7]);
+      L[8] = m2l_fma(D[56], m, L[8]);
     }
-    { const float m = __ldg(Mr + 20);
-      L[1] = fmaf(-D[35], m, L[1]);
-      L[2] = fmaf(-D[38], m, L[2]);
-      L[3] = fmaf(-D[39], m, L[3]);
-      L[4] = fmaf(D[50], m, L[4]);
-      L[5] = fmaf(D[53], m, L[5]);
-      L[6] = fmaf(D[54], m, L[6]);
-      L[7] = fmaf(D[56], m, L[7]);
-      L[8] = fmaf(D[57], m, L[8]);
+    { const T m = __ldg(Mr + 20);
+      L[1] = m2l_fma(-D[35], m, L[1]);
+      L[2] = m2l_fma(-D[38], m, L[2]);
+      L[3] = m2l_fma(-D[39], m, L[3]);
+      L[4] = m2l_fma(D[50], m, L[4]);
+      L[5] = m2l_fma(D[53], m, L[5]);
+      L[6] = m2l_fma(D[54], m, L[6]);
+      L[7] = m2l_fma(D[56], m, L[7]);
+      L[8] = m2l_fma(D[57], m, L[8]);
     }
-    { const float m = __ldg(Mr + 21);
-      L[1] = fmaf(-D[37], m, L[1]);
-      L[2] = fmaf(-D[40], m, L[2]);
-      L[3] = fmaf(-D[41], m, L[3]);
-      L[4] = fmaf(D[52], m, L[4]);
-      L[5] = fmaf(D[55], m, L[5]);
-      L[6] = fmaf(D[56], m, L[6]);
-      L[7] = fmaf(D[58], m, L[7]);
-      L[8] = fmaf(D[59], m, L[8]);
+    { const T m = __ldg(Mr + 21);
+      L[1] = m2l_fma(-D[37], m, L[1]);
+      L[2] = m2l_fma(-D[40], m, L[2]);
+      L[3] = m2l_fma(-D[41], m, L[3]);
+      L[4] = m2l_fma(D[52], m, L[4]);
+      L[5] = m2l_fma(D[55], m, L[5]);
+      L[6] = m2l_fma(D[56], m, L[6]);
+      L[7] = m2l_fma(D[58], m, L[7]);
+      L[8] = m2l_fma(D[59], m, L[8]);
     }
-    { const float m = __ldg(Mr + 22);
-      L[1] = fmaf(-D[38], m, L[1]);
-      L[2] = fmaf(-D[41], m, L[2]);
-      L[3] = fmaf(-D[42], m, L[3]);
-      L[4] = fmaf(D[53], m, L[4]);
-      L[5] = fmaf(D[56], m, L[5]);
-      L[6] = fmaf(D[57], m, L[6]);
-      L[7] = fmaf(D[59], m, L[7]);
-      L[8] = fmaf(D[60], m, L[8]);
+    { const T m = __ldg(Mr + 22);
+      L[1] = m2l_fma(-D[38], m, L[1]);
+      L[2] = m2l_fma(-D[41], m, L[2]);
+      L[3] = m2l_fma(-D[42], m, L[3]);
+      L[4] = m2l_fma(D[53], m, L[4]);
+      L[5] = m2l_fma(D[56], m, L[5]);
+      L[6] = m2l_fma(D[57], m, L[6]);
+      L[7] = m2l_fma(D[59], m, L[7]);
+      L[8] = m2l_fma(D[60], m, L[8]);
     }
-    { const float m = __ldg(Mr + 23);
-      L[1] = fmaf(-D[40], m, L[1]);
-      L[2] = fmaf(-D[43], m, L[2]);
-      L[3] = fmaf(-D[44], m, L[3]);
-      L[4] = fmaf(D[55], m, L[4]);
-      L[5] = fmaf(D[58], m, L[5]);
-      L[6] = fmaf(D[59], m, L[6]);
-      L[7] = fmaf(D[61], m, L[7]);
-      L[8] = fmaf(D[62], m, L[8]);
+    { const T m = __ldg(Mr + 23);
+      L[1] = m2l_fma(-D[40], m, L[1]);
+      L[2] = m2l_fma(-D[43], m, L[2]);
+      L[3] = m2l_fma(-D[44], m, L[3]);
+      L[4] = m2l_fma(D[55], m, L[4]);
+      L[5] = m2l_fma(D[58], m, L[5]);
+      L[6] = m2l_fma(D[59], m, L[6]);
+      L[7] = m2l_fma(D[61], m, L[7]);
+      L[8] = m2l_fma(D[62], m, L[8]);
     }
-    { const float m = __ldg(Mr + 24);
-      L[1] = fmaf(-D[41], m, L[1]);
-      L[2] = fmaf(-D[44], m, L[2]);
-      L[3] = fmaf(-D[45], m, L[3]);
-      L[4] = fmaf(D[56], m, L[4]);
-      L[5] = fmaf(D[59], m, L[5]);
-      L[6] = fmaf(D[60], m, L[6]);
-      L[7] = fmaf(D[62], m, L[7]);
-      L[8] = fmaf(D[63], m, L[8]);
+    { const T m = __ldg(Mr + 24);
+      L[1] = m2l_fma(-D[41], m, L[1]);
+      L[2] = m2l_fma(-D[44], m, L[2]);
+      L[3] = m2l_fma(-D[45], m, L[3]);
+      L[4] = m2l_fma(D[56], m, L[4]);
+      L[5] = m2l_fma(D[59], m, L[5]);
+      L[6] = m2l_fma(D[60], m, L[6]);
+      L[7] = m2l_fma(D[62], m, L[7]);
+      L[8] = m2l_fma(D[63], m, L[8]);
     }
-    { const float m = __ldg(Mr + 25);
-      L[1] = fmaf(-D[46], m, L[1]);
-      L[2] = fmaf(-D[47], m, L[2]);
-      L[3] = fmaf(-D[48], m, L[3]);
+    { const T m = __ldg(Mr + 25);
+      L[1] = m2l_fma(-D[46], m, L[1]);
+      L[2] = m2l_fma(-D[47], m, L[2]);
+      L[3] = m2l_fma(-D[48], m, L[3]);
     }
-    { const float m = __ldg(Mr + 26);
-      L[1] = fmaf(-D[47], m, L[1]);
-      L[2] = fmaf(-D[49], m, L[2]);
-      L[3] = fmaf(-D[50], m, L[3]);
+    { const T m = __ldg(Mr + 26);
+      L[1] = m2l_fma(-D[47], m, L[1]);
+      L[2] = m2l_fma(-D[49], m, L[2]);
+      L[3] = m2l_fma(-D[50], m, L[3]);
     }
-    { const float m = __ldg(Mr + 27);
-      L[1] = fmaf(-D[48], m, L[1]);
-      L[2] = fmaf(-D[50], m, L[2]);
-      L[3] = fmaf(-D[51], m, L[3]);
+    { const T m = __ldg(Mr + 27);
+      L[1] = m2l_fma(-D[48], m, L[1]);
+      L[2] = m2l_fma(-D[50], m, L[2]);
+      L[3] = m2l_fma(-D[51], m, L[3]);
     }
-    { const float m = __ldg(Mr + 28);
-      L[1] = fmaf(-D[49], m, L[1]);
-      L[2] = fmaf(-D[52], m, L[2]);
-      L[3] = fmaf(-D[53], m, L[3]);
+    { const T m = __ldg(Mr + 28);
+      L[1] = m2l_fma(-D[49], m, L[1]);
+      L[2] = m2l_fma(-D[52], m, L[2]);
+      L[3] = m2l_fma(-D[53], m, L[3]);
     }
-    { const float m = __ldg(Mr + 29);
-      L[1] = fmaf(-D[50], m, L[1]);
-      L[2] = fmaf(-D[53], m, L[2]);
-      L[3] = fmaf(-D[54], m, L[3]);
+    { const T m = __ldg(Mr + 29);
+      L[1] = m2l_fma(-D[50], m, L[1]);
+      L[2] = m2l_fma(-D[53], m, L[2]);
+      L[3] = m2l_fma(-D[54], m, L[3]);
     }
-    { const float m = __ldg(Mr + 30);
-      L[1] = fmaf(-D[52], m, L[1]);
-      L[2] = fmaf(-D[55], m, L[2]);
-      L[3] = fmaf(-D[56], m, L[3]);
+    { const T m = __ldg(Mr + 30);
+      L[1] = m2l_fma(-D[52], m, L[1]);
+      L[2] = m2l_fma(-D[55], m, L[2]);
+      L[3] = m2l_fma(-D[56], m, L[3]);
     }
-    { const float m = __ldg(Mr + 31);
-      L[1] = fmaf(-D[53], m, L[1]);
-      L[2] = fmaf(-D[56], m, L[2]);
-      L[3] = fmaf(-D[57], m, L[3]);
+    { const T m = __ldg(Mr + 31);
+      L[1] = m2l_fma(-D[53], m, L[1]);
+      L[2] = m2l_fma(-D[56], m, L[2]);
+      L[3] = m2l_fma(-D[57], m, L[3]);
     }
-    { const float m = __ldg(Mr + 32);
-      L[1] = fmaf(-D[55], m, L[1]);
-      L[2] = fmaf(-D[58], m, L[2]);
-      L[3] = fmaf(-D[59], m, L[3]);
+    { const T m = __ldg(Mr + 32);
+      L[1] = m2l_fma(-D[55], m, L[1]);
+      L[2] = m2l_fma(-D[58], m, L[2]);
+      L[3] = m2l_fma(-D[59], m, L[3]);
     }
-    { const float m = __ldg(Mr + 33);
-      L[1] = fmaf(-D[56], m, L[1]);
-      L[2] = fmaf(-D[59], m, L[2]);
-      L[3] = fmaf(-D[60], m, L[3]);
+    { const T m = __ldg(Mr + 33);
+      L[1] = m2l_fma(-D[56], m, L[1]);
+      L[2] = m2l_fma(-D[59], m, L[2]);
+      L[3] = m2l_fma(-D[60], m, L[3]);
     }
-    { const float m = __ldg(Mr + 34);
-      L[1] = fmaf(-D[58], m, L[1]);
-      L[2] = fmaf(-D[61], m, L[2]);
-      L[3] = fmaf(-D[62], m, L[3]);
+    { const T m = __ldg(Mr + 34);
+      L[1] = m2l_fma(-D[58], m, L[1]);
+      L[2] = m2l_fma(-D[61], m, L[2]);
+      L[3] = m2l_fma(-D[62], m, L[3]);
     }
-    { const float m = __ldg(Mr + 35);
-      L[1] = fmaf(-D[59], m, L[1]);
-      L[2] = fmaf(-D[62], m, L[2]);
-      L[3] = fmaf(-D[63], m, L[3]);
+    { const T m = __ldg(Mr + 35);
+      L[1] = m2l_fma(-D[59], m, L[1]);
+      L[2] = m2l_fma(-D[62], m, L[2]);
+      L[3] = m2l_fma(-D[63], m, L[3]);
     }
 }
 
-__device__ __forceinline__ void m2l_reduce_moments_h_6(const float *__restrict__ Ms, float *__restrict__ Mr)
+template <class T> __device__ __forceinline__ void m2l_reduce_moments_h_6(const T *__restrict__ Ms, T *__restrict__ Mr)
 {
-    float v0 = Ms[0];
-    float v1 = Ms[1];
-    float v2 = Ms[2];
-    float v3 = Ms[3];
-    float v4 = Ms[4];
-    float v5 = Ms[5];
-    float v6 = Ms[6];
-    float v7 = Ms[7];
-    float v8 = Ms[8];
-    float v9 = Ms[9];
-    float v10 = Ms[10];
-    float v11 = Ms[11];
-    float v12 = Ms[12];
-    float v13 = Ms[13];
-    float v14 = Ms[14];
-    float v15 = Ms[15];
-    float v16 = Ms[16];
-    float v17 = Ms[17];
-    float v18 = Ms[18];
-    float v19 = Ms[19];
-    float v20 = Ms[20];
-    float v21 = Ms[21];
-    float v22 = Ms[22];
-    float v23 = Ms[23];
-    float v24 = Ms[24];
-    float v25 = Ms[25];
-    float v26 = Ms[26];
-    float v27 = Ms[27];
-    float v28 = Ms[28];
-    float v29 = Ms[29];
-    float v30 = Ms[30];
-    float v31 = Ms[31];
-    float v32 = Ms[32];
-    float v33 = Ms[33];
-    float v34 = Ms[34];
-    float v35 = Ms[35];
-    float v36 = Ms[36];
-    float v37 = Ms[37];
-    float v38 = Ms[38];
-    float v39 = Ms[39];
-    float v40 = Ms[40];
-    float v41 = Ms[41];
-    float v42 = Ms[42];
-    float v43 = Ms[43];
-    float v44 = Ms[44];
-    float v45 = Ms[45];
-    float v46 = Ms[46];
-    float v47 = Ms[47];
-    float v48 = Ms[48];
-    float v49 = Ms[49];
-    float v50 = Ms[50];
-    float v51 = Ms[51];
-    float v52 = Ms[52];
-    float v53 = Ms[53];
-    float v54 = Ms[54];
-    float v55 = Ms[55];
-    float v56 = Ms[56];
-    float v57 = Ms[57];
-    float v58 = Ms[58];
-    float v59 = Ms[59];
-    float v60 = Ms[60];
-    float v61 = Ms[61];
-    float v62 = Ms[62];
-    float v63 = Ms[63];
-    float v64 = Ms[64];
-    float v65 = Ms[65];
-    float v66 = Ms[66];
-    float v67 = Ms[67];
-    float v68 = Ms[68];
-    float v69 = Ms[69];
-    float v70 = Ms[70];
-    float v71 = Ms[71];
-    float v72 = Ms[72];
-    float v73 = Ms[73];
-    float v74 = Ms[74];
-    float v75 = Ms[75];
-    float v76 = Ms[76];
-    float v77 = Ms[77];
-    float v78 = Ms[78];
-    float v79 = Ms[79];
-    float v80 = Ms[80];
-    float v81 = Ms[81];
-    float v82 = Ms[82];
-    float v83 = Ms[83];
+    T v0 = Ms[0];
+    T v1 = Ms[1];
+    T v2 = Ms[2];
+    T v3 = Ms[3];
+    T v4 = Ms[4];
+    T v5 = Ms[5];
+    T v6 = Ms[6];
+    T v7 = Ms[7];
+    T v8 = Ms[8];
+    T v9 = Ms[9];
+    T v10 = Ms[10];
+    T v11 = Ms[11];
+    T v12 = Ms[12];
+    T v13 = Ms[13];
+    T v14 = Ms[14];
+    T v15 = Ms[15];
+    T v16 = Ms[16];
+    T v17 = Ms[17];
+    T v18 = Ms[18];
+    T v19 = Ms[19];
+    T v20 = Ms[20];
+    T v21 = Ms[21];
+    T v22 = Ms[22];
+    T v23 = Ms[23];
+    T v24 = Ms[24];
+    T v25 = Ms[25];
+    T v26 = Ms[26];
+    T v27 = Ms[27];
+    T v28 = Ms[28];
+    T v29 = Ms[29];
+    T v30 = Ms[30];
+    T v31 = Ms[31];
+    T v32 = Ms[32];
+    T v33 = Ms[33];
+    T v34 = Ms[34];
+    T v35 = Ms[35];
+    T v36 = Ms[36];
+    T v37 = Ms[37];
+    T v38 = Ms[38];
+    T v39 = Ms[39];
+    T v40 = Ms[40];
+    T v41 = Ms[41];
+    T v42 = Ms[42];
+    T v43 = Ms[43];
+    T v44 = Ms[44];
+    T v45 = Ms[45];
+    T v46 = Ms[46];
+    T v47 = Ms[47];
+    T v48 = Ms[48];
+    T v49 = Ms[49];
+    T v50 = Ms[50];
+    T v51 = Ms[51];
+    T v52 = Ms[52];
+    T v53 = Ms[53];
+    T v54 = Ms[54];
+    T v55 = Ms[55];
+    T v56 = Ms[56];
+    T v57 = Ms[57];
+    T v58 = Ms[58];
+    T v59 = Ms[59];
+    T v60 = Ms[60];
+    T v61 = Ms[61];
+    T v62 = Ms[62];
+    T v63 = Ms[63];
+    T v64 = Ms[64];
+    T v65 = Ms[65];
+    T v66 = Ms[66];
+    T v67 = Ms[67];
+    T v68 = Ms[68];
+    T v69 = Ms[69];
+    T v70 = Ms[70];
+    T v71 = Ms[71];
+    T v72 = Ms[72];
+    T v73 = Ms[73];
+    T v74 = Ms[74];
+    T v75 = Ms[75];
+    T v76 = Ms[76];
+    T v77 = Ms[77];
+    T v78 = Ms[78];
+    T v79 = Ms[79];
+    T v80 = Ms[80];
+    T v81 = Ms[81];
+    T v82 = Ms[82];
+    T v83 = Ms[83];
     v70 -= v83;
     v81 -= v83;
     v44 -= v55;
@@ -17734,175 +17733,175 @@ __device__ __forceinline__ void m2l_reduce_moments_h_6(const float *__restrict__
     Mr[48] = v78;
 }
 
-__device__ __forceinline__ void m2l_complete_locals_h_6(const float *__restrict__ Lr, float *__restrict__ L)
+template <class T> __device__ __forceinline__ void m2l_complete_locals_h_6(const T *__restrict__ Lr, T *__restrict__ L)
 {
-    const float v0 = Lr[0];
+    const T v0 = Lr[0];
     L[0] = v0;
-    const float v1 = Lr[1];
+    const T v1 = Lr[1];
     L[1] = v1;
-    const float v2 = Lr[2];
+    const T v2 = Lr[2];
     L[2] = v2;
-    const float v3 = Lr[3];
+    const T v3 = Lr[3];
     L[3] = v3;
-    const float v4 = Lr[4];
+    const T v4 = Lr[4];
     L[4] = v4;
-    const float v5 = Lr[5];
+    const T v5 = Lr[5];
     L[5] = v5;
-    const float v6 = Lr[6];
+    const T v6 = Lr[6];
     L[6] = v6;
-    const float v7 = Lr[7];
+    const T v7 = Lr[7];
     L[7] = v7;
-    const float v8 = Lr[8];
+    const T v8 = Lr[8];
     L[8] = v8;
-    const float v9 = -v4 - v7;
+    const T v9 = -v4 - v7;
     L[9] = v9;
-    const float v10 = Lr[9];
+    const T v10 = Lr[9];
     L[10] = v10;
-    const float v11 = Lr[10];
+    const T v11 = Lr[10];
     L[11] = v11;
-    const float v12 = Lr[11];
+    const T v12 = Lr[11];
     L[12] = v12;
-    const float v13 = Lr[12];
+    const T v13 = Lr[12];
     L[13] = v13;
-    const float v14 = Lr[13];
+    const T v14 = Lr[13];
     L[14] = v14;
-    const float v15 = -v10 - v13;
+    const T v15 = -v10 - v13;
     L[15] = v15;
-    const float v16 = Lr[14];
+    const T v16 = Lr[14];
     L[16] = v16;
-    const float v17 = Lr[15];
+    const T v17 = Lr[15];
     L[17] = v17;
-    const float v18 = -v11 - v16;
+    const T v18 = -v11 - v16;
     L[18] = v18;
-    const float v19 = -v12 - v17;
+    const T v19 = -v12 - v17;
     L[19] = v19;
-    const float v20 = Lr[16];
+    const T v20 = Lr[16];
     L[20] = v20;
-    const float v21 = Lr[17];
+    const T v21 = Lr[17];
     L[21] = v21;
-    const float v22 = Lr[18];
+    const T v22 = Lr[18];
     L[22] = v22;
-    const float v23 = Lr[19];
+    const T v23 = Lr[19];
     L[23] = v23;
-    const float v24 = Lr[20];
+    const T v24 = Lr[20];
     L[24] = v24;
-    const float v25 = -v20 - v23;
+    const T v25 = -v20 - v23;
     L[25] = v25;
-    const float v26 = Lr[21];
+    const T v26 = Lr[21];
     L[26] = v26;
-    const float v27 = Lr[22];
+    const T v27 = Lr[22];
     L[27] = v27;
-    const float v28 = -v21 - v26;
+    const T v28 = -v21 - v26;
     L[28] = v28;
-    const float v29 = -v22 - v27;
+    const T v29 = -v22 - v27;
     L[29] = v29;
-    const float v30 = Lr[23];
+    const T v30 = Lr[23];
     L[30] = v30;
-    const float v31 = Lr[24];
+    const T v31 = Lr[24];
     L[31] = v31;
-    const float v32 = -v23 - v30;
+    const T v32 = -v23 - v30;
     L[32] = v32;
-    const float v33 = -v24 - v31;
+    const T v33 = -v24 - v31;
     L[33] = v33;
-    const float v34 = -v25 - v32;
+    const T v34 = -v25 - v32;
     L[34] = v34;
-    const float v35 = Lr[25];
+    const T v35 = Lr[25];
     L[35] = v35;
-    const float v36 = Lr[26];
+    const T v36 = Lr[26];
     L[36] = v36;
-    const float v37 = Lr[27];
+    const T v37 = Lr[27];
     L[37] = v37;
-    const float v38 = Lr[28];
+    const T v38 = Lr[28];
     L[38] = v38;
-    const float v39 = Lr[29];
+    const T v39 = Lr[29];
     L[39] = v39;
-    const float v40 = -v35 - v38;
+    const T v40 = -v35 - v38;
     L[40] = v40;
-    const float v41 = Lr[30];
+    const T v41 = Lr[30];
     L[41] = v41;
-    const float v42 = Lr[31];
+    const T v42 = Lr[31];
     L[42] = v42;
-    const float v43 = -v36 - v41;
+    const T v43 = -v36 - v41;
     L[43] = v43;
-    const float v44 = -v37 - v42;
+    const T v44 = -v37 - v42;
     L[44] = v44;
-    const float v45 = Lr[32];
+    const T v45 = Lr[32];
     L[45] = v45;
-    const float v46 = Lr[33];
+    const T v46 = Lr[33];
     L[46] = v46;
-    const float v47 = -v38 - v45;
+    const T v47 = -v38 - v45;
     L[47] = v47;
-    const float v48 = -v39 - v46;
+    const T v48 = -v39 - v46;
     L[48] = v48;
-    const float v49 = -v40 - v47;
+    const T v49 = -v40 - v47;
     L[49] = v49;
-    const float v50 = Lr[34];
+    const T v50 = Lr[34];
     L[50] = v50;
-    const float v51 = Lr[35];
+    const T v51 = Lr[35];
     L[51] = v51;
-    const float v52 = -v41 - v50;
+    const T v52 = -v41 - v50;
     L[52] = v52;
-    const float v53 = -v42 - v51;
+    const T v53 = -v42 - v51;
     L[53] = v53;
-    const float v54 = -v43 - v52;
+    const T v54 = -v43 - v52;
     L[54] = v54;
-    const float v55 = -v44 - v53;
+    const T v55 = -v44 - v53;
     L[55] = v55;
-    const float v56 = Lr[36];
+    const T v56 = Lr[36];
     L[56] = v56;
-    const float v57 = Lr[37];
+    const T v57 = Lr[37];
     L[57] = v57;
-    const float v58 = Lr[38];
+    const T v58 = Lr[38];
     L[58] = v58;
-    const float v59 = Lr[39];
+    const T v59 = Lr[39];
     L[59] = v59;
-    const float v60 = Lr[40];
+    const T v60 = Lr[40];
     L[60] = v60;
-    const float v61 = -v56 - v59;
+    const T v61 = -v56 - v59;
     L[61] = v61;
-    const float v62 = Lr[41];
+    const T v62 = Lr[41];
     L[62] = v62;
-    const float v63 = Lr[42];
+    const T v63 = Lr[42];
     L[63] = v63;
-    const float v64 = -v57 - v62;
+    const T v64 = -v57 - v62;
     L[64] = v64;
-    const float v65 = -v58 - v63;
+    const T v65 = -v58 - v63;
     L[65] = v65;
-    const float v66 = Lr[43];
+    const T v66 = Lr[43];
     L[66] = v66;
-    const float v67 = Lr[44];
+    const T v67 = Lr[44];
     L[67] = v67;
-    const float v68 = -v59 - v66;
+    const T v68 = -v59 - v66;
     L[68] = v68;
-    const float v69 = -v60 - v67;
+    const T v69 = -v60 - v67;
     L[69] = v69;
-    const float v70 = -v61 - v68;
+    const T v70 = -v61 - v68;
     L[70] = v70;
-    const float v71 = Lr[45];
+    const T v71 = Lr[45];
     L[71] = v71;
-    const float v72 = Lr[46];
+    const T v72 = Lr[46];
     L[72] = v72;
-    const float v73 = -v62 - v71;
+    const T v73 = -v62 - v71;
     L[73] = v73;
-    const float v74 = -v63 - v72;
+    const T v74 = -v63 - v72;
     L[74] = v74;
-    const float v75 = -v64 - v73;
+    const T v75 = -v64 - v73;
     L[75] = v75;
-    const float v76 = -v65 - v74;
+    const T v76 = -v65 - v74;
     L[76] = v76;
-    const float v77 = Lr[47];
+    const T v77 = Lr[47];
     L[77] = v77;
-    const float v78 = Lr[48];
+    const T v78 = Lr[48];
     L[78] = v78;
-    const float v79 = -v66 - v77;
+    const T v79 = -v66 - v77;
     L[79] = v79;
-    const float v80 = -v67 - v78;
+    const T v80 = -v67 - v78;
     L[80] = v80;
-    const float v81 = -v68 - v79;
+    const T v81 = -v68 - v79;
     L[81] = v81;
-    const float v82 = -v69 - v80;
+    const T v82 = -v69 - v80;
     L[82] = v82;
-    const float v83 = -v70 - v81;
+    const T v83 = -v70 - v81;
     L[83] = v83;
 }
 
@@ -17910,78 +17909,78 @@ template <int P> struct M2LGenH;
 template <> struct M2LGenH<1> {
     static constexpr int NC = 4;
     static constexpr int ND = 4;
-    static __device__ __forceinline__ void dtensor(float dx, float dy, float dz, float (&D)[4]) { m2l_dtensor_h_1(dx, dy, dz, D); }
-    static __device__ __forceinline__ void side_a(const float (&D)[4], const float *Mr, float rho, float (&L)[4]) { m2l_side_a_h_1(D, Mr, rho, L); }
-    static __device__ __forceinline__ void side_b(const float (&D)[4], const float *Mr, float (&L)[4]) { m2l_side_b_h_1(D, Mr, L); }
-    static __device__ __forceinline__ void side_a_forces(const float (&D)[4], const float *Mr, float rho, float (&L)[4]) { m2l_side_a_h_forces_1(D, Mr, rho, L); }
-    static __device__ __forceinline__ void side_b_forces(const float (&D)[4], const float *Mr, float (&L)[4]) { m2l_side_b_h_forces_1(D, Mr, L); }
-    static __device__ __forceinline__ void acc(const float (&D)[4], const float *Mr, float rho, float (&L)[4]) { m2l_acc_h_1(D, Mr, rho, L); }
-    static __device__ __forceinline__ void acc_forces(const float (&D)[4], const float *Mr, float rho, float (&L)[4]) { m2l_acc_h_forces_1(D, Mr, rho, L); }
-    static __device__ __forceinline__ void reduce_moments(const float *Ms, float *Mr) { m2l_reduce_moments_h_1(Ms, Mr); }
-    static __device__ __forceinline__ void complete_locals(const float *Lr, float *L) { m2l_complete_locals_h_1(Lr, L); }
+    template <class T> static __device__ __forceinline__ void dtensor(T dx, T dy, T dz, T (&D)[4]) { m2l_dtensor_h_1(dx, dy, dz, D); }
+    template <class T> static __device__ __forceinline__ void side_a(const T (&D)[4], const T *Mr, T rho, T (&L)[4]) { m2l_side_a_h_1(D, Mr, rho, L); }
+    template <class T> static __device__ __forceinline__ void side_b(const T (&D)[4], const T *Mr, T (&L)[4]) { m2l_side_b_h_1(D, Mr, L); }
+    template <class T> static __device__ __forceinline__ void side_a_forces(const T (&D)[4], const T *Mr, T rho, T (&L)[4]) { m2l_side_a_h_forces_1(D, Mr, rho, L); }
+    template <class T> static __device__ __forceinline__ void side_b_forces(const T (&D)[4], const T *Mr, T (&L)[4]) { m2l_side_b_h_forces_1(D, Mr, L); }
+    template <class T> static __device__ __forceinline__ void acc(const T (&D)[4], const T *Mr, T rho, T (&L)[4]) { m2l_acc_h_1(D, Mr, rho, L); }
+    template <class T> static __device__ __forceinline__ void acc_forces(const T (&D)[4], const T *Mr, T rho, T (&L)[4]) { m2l_acc_h_forces_1(D, Mr, rho, L); }
+    template <class T> static __device__ __forceinline__ void reduce_moments(const T *Ms, T *Mr) { m2l_reduce_moments_h_1(Ms, Mr); }
+    template <class T> static __device__ __forceinline__ void complete_locals(const T *Lr, T *L) { m2l_complete_locals_h_1(Lr, L); }
 };
 template <> struct M2LGenH<2> {
     static constexpr int NC = 9;
     static constexpr int ND = 10;
-    static __device__ __forceinline__ void dtensor(float dx, float dy, float dz, float (&D)[10]) { m2l_dtensor_h_2(dx, dy, dz, D); }
-    static __device__ __forceinline__ void side_a(const float (&D)[10], const float *Mr, float rho, float (&L)[9]) { m2l_side_a_h_2(D, Mr, rho, L); }
-    static __device__ __forceinline__ void side_b(const float (&D)[10], const float *Mr, float (&L)[9]) { m2l_side_b_h_2(D, Mr, L); }
-    static __device__ __forceinline__ void side_a_forces(const float (&D)[10], const float *Mr, float rho, float (&L)[9]) { m2l_side_a_h_forces_2(D, Mr, rho, L); }
-    static __device__ __forceinline__ void side_b_forces(const float (&D)[10], const float *Mr, float (&L)[9]) { m2l_side_b_h_forces_2(D, Mr, L); }
-    static __device__ __forceinline__ void acc(const float (&D)[10], const float *Mr, float rho, float (&L)[9]) { m2l_acc_h_2(D, Mr, rho, L); }
-    static __device__ __forceinline__ void acc_forces(const float (&D)[10], const float *Mr, float rho, float (&L)[9]) { m2l_acc_h_forces_2(D, Mr, rho, L); }
-    static __device__ __forceinline__ void reduce_moments(const float *Ms, float *Mr) { m2l_reduce_moments_h_2(Ms, Mr); }
-    static __device__ __forceinline__ void complete_locals(const float *Lr, float *L) { m2l_complete_locals_h_2(Lr, L); }
+    template <class T> static __device__ __forceinline__ void dtensor(T dx, T dy, T dz, T (&D)[10]) { m2l_dtensor_h_2(dx, dy, dz, D); }
+    template <class T> static __device__ __forceinline__ void side_a(const T (&D)[10], const T *Mr, T rho, T (&L)[9]) { m2l_side_a_h_2(D, Mr, rho, L); }
+    template <class T> static __device__ __forceinline__ void side_b(const T (&D)[10], const T *Mr, T (&L)[9]) { m2l_side_b_h_2(D, Mr, L); }
+    template <class T> static __device__ __forceinline__ void side_a_forces(const T (&D)[10], const T *Mr, T rho, T (&L)[9]) { m2l_side_a_h_forces_2(D, Mr, rho, L); }
+    template <class T> static __device__ __forceinline__ void side_b_forces(const T (&D)[10], const T *Mr, T (&L)[9]) { m2l_side_b_h_forces_2(D, Mr, L); }
+    template <class T> static __device__ __forceinline__ void acc(const T (&D)[10], const T *Mr, T rho, T (&L)[9]) { m2l_acc_h_2(D, Mr, rho, L); }
+    template <class T> static __device__ __forceinline__ void acc_forces(const T (&D)[10], const T *Mr, T rho, T (&L)[9]) { m2l_acc_h_forces_2(D, Mr, rho, L); }
+    template <class T> static __device__ __forceinline__ void reduce_moments(const T *Ms, T *Mr) { m2l_reduce_moments_h_2(Ms, Mr); }
+    template <class T> static __device__ __forceinline__ void complete_locals(const T *Lr, T *L) { m2l_complete_locals_h_2(Lr, L); }
 };
 template <> struct M2LGenH<3> {
     static constexpr int NC = 16;
     static constexpr int ND = 19;
-    static __device__ __forceinline__ void dtensor(float dx, float dy, float dz, float (&D)[19]) { m2l_dtensor_h_3(dx, dy, dz, D); }
-    static __device__ __forceinline__ void side_a(const float (&D)[19], const float *Mr, float rho, float (&L)[16]) { m2l_side_a_h_3(D, Mr, rho, L); }
-    static __device__ __forceinline__ void side_b(const float (&D)[19], const float *Mr, float (&L)[16]) { m2l_side_b_h_3(D, Mr, L); }
-    static __device__ __forceinline__ void side_a_forces(const float (&D)[19], const float *Mr, float rho, float (&L)[16]) { m2l_side_a_h_forces_3(D, Mr, rho, L); }
-    static __device__ __forceinline__ void side_b_forces(const float (&D)[19], const float *Mr, float (&L)[16]) { m2l_side_b_h_forces_3(D, Mr, L); }
-    static __device__ __forceinline__ void acc(const float (&D)[19], const float *Mr, float rho, float (&L)[16]) { m2l_acc_h_3(D, Mr, rho, L); }
-    static __device__ __forceinline__ void acc_forces(const float (&D)[19], const float *Mr, float rho, float (&L)[16]) { m2l_acc_h_forces_3(D, Mr, rho, L); }
-    static __device__ __forceinline__ void reduce_moments(const float *Ms, float *Mr) { m2l_reduce_moments_h_3(Ms, Mr); }
-    static __device__ __forceinline__ void complete_locals(const float *Lr, float *L) { m2l_complete_locals_h_3(Lr, L); }
+    template <class T> static __device__ __forceinline__ void dtensor(T dx, T dy, T dz, T (&D)[19]) { m2l_dtensor_h_3(dx, dy, dz, D); }
+    template <class T> static __device__ __forceinline__ void side_a(const T (&D)[19], const T *Mr, T rho, T (&L)[16]) { m2l_side_a_h_3(D, Mr, rho, L); }
+    template <class T> static __device__ __forceinline__ void side_b(const T (&D)[19], const T *Mr, T (&L)[16]) { m2l_side_b_h_3(D, Mr, L); }
+    template <class T> static __device__ __forceinline__ void side_a_forces(const T (&D)[19], const T *Mr, T rho, T (&L)[16]) { m2l_side_a_h_forces_3(D, Mr, rho, L); }
+    template <class T> static __device__ __forceinline__ void side_b_forces(const T (&D)[19], const T *Mr, T (&L)[16]) { m2l_side_b_h_forces_3(D, Mr, L); }
+    template <class T> static __device__ __forceinline__ void acc(const T (&D)[19], const T *Mr, T rho, T (&L)[16]) { m2l_acc_h_3(D, Mr, rho, L); }
+    template <class T> static __device__ __forceinline__ void acc_forces(const T (&D)[19], const T *Mr, T rho, T (&L)[16]) { m2l_acc_h_forces_3(D, Mr, rho, L); }
+    template <class T> static __device__ __forceinline__ void reduce_moments(const T *Ms, T *Mr) { m2l_reduce_moments_h_3(Ms, Mr); }
+    template <class T> static __device__ __forceinline__ void complete_locals(const T *Lr, T *L) { m2l_complete_locals_h_3(Lr, L); }
 };
 template <> struct M2LGenH<4> {
     static constexpr int NC = 25;
     static constexpr int ND = 31;
-    static __device__ __forceinline__ void dtensor(float dx, float dy, float dz, float (&D)[31]) { m2l_dtensor_h_4(dx, dy, dz, D); }
-    static __device__ __forceinline__ void side_a(const float (&D)[31], const float *Mr, float rho, float (&L)[25]) { m2l_side_a_h_4(D, Mr, rho, L); }
-    static __device__ __forceinline__ void side_b(const float (&D)[31], const float *Mr, float (&L)[25]) { m2l_side_b_h_4(D, Mr, L); }
-    static __device__ __forceinline__ void side_a_forces(const float (&D)[31], const float *Mr, float rho, float (&L)[25]) { m2l_side_a_h_forces_4(D, Mr, rho, L); }
-    static __device__ __forceinline__ void side_b_forces(const float (&D)[31], const float *Mr, float (&L)[25]) { m2l_side_b_h_forces_4(D, Mr, L); }
-    static __device__ __forceinline__ void acc(const float (&D)[31], const float *Mr, float rho, float (&L)[25]) { m2l_acc_h_4(D, Mr, rho, L); }
-    static __device__ __forceinline__ void acc_forces(const float (&D)[31], const float *Mr, float rho, float (&L)[25]) { m2l_acc_h_forces_4(D, Mr, rho, L); }
-    static __device__ __forceinline__ void reduce_moments(const float *Ms, float *Mr) { m2l_reduce_moments_h_4(Ms, Mr); }
-    static __device__ __forceinline__ void complete_locals(const float *Lr, float *L) { m2l_complete_locals_h_4(Lr, L); }
+    template <class T> static __device__ __forceinline__ void dtensor(T dx, T dy, T dz, T (&D)[31]) { m2l_dtensor_h_4(dx, dy, dz, D); }
+    template <class T> static __device__ __forceinline__ void side_a(const T (&D)[31], const T *Mr, T rho, T (&L)[25]) { m2l_side_a_h_4(D, Mr, rho, L); }
+    template <class T> static __device__ __forceinline__ void side_b(const T (&D)[31], const T *Mr, T (&L)[25]) { m2l_side_b_h_4(D, Mr, L); }
+    template <class T> static __device__ __forceinline__ void side_a_forces(const T (&D)[31], const T *Mr, T rho, T (&L)[25]) { m2l_side_a_h_forces_4(D, Mr, rho, L); }
+    template <class T> static __device__ __forceinline__ void side_b_forces(const T (&D)[31], const T *Mr, T (&L)[25]) { m2l_side_b_h_forces_4(D, Mr, L); }
+    template <class T> static __device__ __forceinline__ void acc(const T (&D)[31], const T *Mr, T rho, T (&L)[25]) { m2l_acc_h_4(D, Mr, rho, L); }
+    template <class T> static __device__ __forceinline__ void acc_forces(const T (&D)[31], const T *Mr, T rho, T (&L)[25]) { m2l_acc_h_forces_4(D, Mr, rho, L); }
+    template <class T> static __device__ __forceinline__ void reduce_moments(const T *Ms, T *Mr) { m2l_reduce_moments_h_4(Ms, Mr); }
+    template <class T> static __device__ __forceinline__ void complete_locals(const T *Lr, T *L) { m2l_complete_locals_h_4(Lr, L); }
 };
 template <> struct M2LGenH<5> {
     static constexpr int NC = 36;
     static constexpr int ND = 46;
-    static __device__ __forceinline__ void dtensor(float dx, float dy, float dz, float (&D)[46]) { m2l_dtensor_h_5(dx, dy, dz, D); }
-    static __device__ __forceinline__ void side_a(const float (&D)[46], const float *Mr, float rho, float (&L)[36]) { m2l_side_a_h_5(D, Mr, rho, L); }
-    static __device__ __forceinline__ void side_b(const float (&D)[46], const float *Mr, float (&L)[36]) { m2l_side_b_h_5(D, Mr, L); }
-    static __device__ __forceinline__ void side_a_forces(const float (&D)[46], const float *Mr, float rho, float (&L)[36]) { m2l_side_a_h_forces_5(D, Mr, rho, L); }
-    static __device__ __forceinline__ void side_b_forces(const float (&D)[46], const float *Mr, float (&L)[36]) { m2l_side_b_h_forces_5(D, Mr, L); }
-    static __device__ __forceinline__ void acc(const float (&D)[46], const float *Mr, float rho, float (&L)[36]) { m2l_acc_h_5(D, Mr, rho, L); }
-    static __device__ __forceinline__ void acc_forces(const float (&D)[46], const float *Mr, float rho, float (&L)[36]) { m2l_acc_h_forces_5(D, Mr, rho, L); }
-    static __device__ __forceinline__ void reduce_moments(const float *Ms, float *Mr) { m2l_reduce_moments_h_5(Ms, Mr); }
-    static __device__ __forceinline__ void complete_locals(const float *Lr, float *L) { m2l_complete_locals_h_5(Lr, L); }
+    template <class T> static __device__ __forceinline__ void dtensor(T dx, T dy, T dz, T (&D)[46]) { m2l_dtensor_h_5(dx, dy, dz, D); }
+    template <class T> static __device__ __forceinline__ void side_a(const T (&D)[46], const T *Mr, T rho, T (&L)[36]) { m2l_side_a_h_5(D, Mr, rho, L); }
+    template <class T> static __device__ __forceinline__ void side_b(const T (&D)[46], const T *Mr, T (&L)[36]) { m2l_side_b_h_5(D, Mr, L); }
+    template <class T> static __device__ __forceinline__ void side_a_forces(const T (&D)[46], const T *Mr, T rho, T (&L)[36]) { m2l_side_a_h_forces_5(D, Mr, rho, L); }
+    template <class T> static __device__ __forceinline__ void side_b_forces(const T (&D)[46], const T *Mr, T (&L)[36]) { m2l_side_b_h_forces_5(D, Mr, L); }
+    template <class T> static __device__ __forceinline__ void acc(const T (&D)[46], const T *Mr, T rho, T (&L)[36]) { m2l_acc_h_5(D, Mr, rho, L); }
+    template <class T> static __device__ __forceinline__ void acc_forces(const T (&D)[46], const T *Mr, T rho, T (&L)[36]) { m2l_acc_h_forces_5(D, Mr, rho, L); }
+    template <class T> static __device__ __forceinline__ void reduce_moments(const T *Ms, T *Mr) { m2l_reduce_moments_h_5(Ms, Mr); }
+    template <class T> static __device__ __forceinline__ void complete_locals(const T *Lr, T *L) { m2l_complete_locals_h_5(Lr, L); }
 };
 template <> struct M2LGenH<6> {
     static constexpr int NC = 49;
     static constexpr int ND = 64;
-    static __device__ __forceinline__ void dtensor(float dx, float dy, float dz, float (&D)[64]) { m2l_dtensor_h_6(dx, dy, dz, D); }
-    static __device__ __forceinline__ void side_a(const float (&D)[64], const float *Mr, float rho, float (&L)[49]) { m2l_side_a_h_6(D, Mr, rho, L); }
-    static __device__ __forceinline__ void side_b(const float (&D)[64], const float *Mr, float (&L)[49]) { m2l_side_b_h_6(D, Mr, L); }
-    static __device__ __forceinline__ void side_a_forces(const float (&D)[64], const float *Mr, float rho, float (&L)[49]) { m2l_side_a_h_forces_6(D, Mr, rho, L); }
-    static __device__ __forceinline__ void side_b_forces(const float (&D)[64], const float *Mr, float (&L)[49]) { m2l_side_b_h_forces_6(D, Mr, L); }
-    static __device__ __forceinline__ void acc(const float (&D)[64], const float *Mr, float rho, float (&L)[49]) { m2l_acc_h_6(D, Mr, rho, L); }
-    static __device__ __forceinline__ void acc_forces(const float (&D)[64], const float *Mr, float rho, float (&L)[49]) { m2l_acc_h_forces_6(D, Mr, rho, L); }
-    static __device__ __forceinline__ void reduce_moments(const float *Ms, float *Mr) { m2l_reduce_moments_h_6(Ms, Mr); }
-    static __device__ __forceinline__ void complete_locals(const float *Lr, float *L) { m2l_complete_locals_h_6(Lr, L); }
+    template <class T> static __device__ __forceinline__ void dtensor(T dx, T dy, T dz, T (&D)[64]) { m2l_dtensor_h_6(dx, dy, dz, D); }
+    template <class T> static __device__ __forceinline__ void side_a(const T (&D)[64], const T *Mr, T rho, T (&L)[49]) { m2l_side_a_h_6(D, Mr, rho, L); }
+    template <class T> static __device__ __forceinline__ void side_b(const T (&D)[64], const T *Mr, T (&L)[49]) { m2l_side_b_h_6(D, Mr, L); }
+    template <class T> static __device__ __forceinline__ void side_a_forces(const T (&D)[64], const T *Mr, T rho, T (&L)[49]) { m2l_side_a_h_forces_6(D, Mr, rho, L); }
+    template <class T> static __device__ __forceinline__ void side_b_forces(const T (&D)[64], const T *Mr, T (&L)[49]) { m2l_side_b_h_forces_6(D, Mr, L); }
+    template <class T> static __device__ __forceinline__ void acc(const T (&D)[64], const T *Mr, T rho, T (&L)[49]) { m2l_acc_h_6(D, Mr, rho, L); }
+    template <class T> static __device__ __forceinline__ void acc_forces(const T (&D)[64], const T *Mr, T rho, T (&L)[49]) { m2l_acc_h_forces_6(D, Mr, rho, L); }
+    template <class T> static __device__ __forceinline__ void reduce_moments(const T *Ms, T *Mr) { m2l_reduce_moments_h_6(Ms, Mr); }
+    template <class T> static __device__ __forceinline__ void complete_locals(const T *Lr, T *L) { m2l_complete_locals_h_6(Lr, L); }
 };

@@ -46,7 +46,8 @@ template <int P>
 struct M2LFull : M2LGen<P> {
     static constexpr int ND = M2LGen<P>::NC;
     static constexpr bool HARMONIC = false;
-    static __device__ __forceinline__ void dt(float dx, float dy, float dz, float soft2, float (&D)[ND])
+    template <class T>
+    static __device__ __forceinline__ void dt(T dx, T dy, T dz, T soft2, T (&D)[ND])
     {
         M2LGen<P>::dtensor(dx, dy, dz, soft2, D);
     }
@@ -55,7 +56,8 @@ template <int P>
 struct M2LHarm : M2LGenH<P> {
     static constexpr int ND = M2LGenH<P>::ND;
     static constexpr bool HARMONIC = true;
-    static __device__ __forceinline__ void dt(float dx, float dy, float dz, float, float (&D)[ND])
+    template <class T>
+    static __device__ __forceinline__ void dt(T dx, T dy, T dz, T, T (&D)[ND])
     {
         M2LGenH<P>::dtensor(dx, dy, dz, D);
     }
@@ -74,27 +76,27 @@ __host__ __device__ constexpr int order_in(bool harmonic, int k)
 }
 
 // per cell and class: fold the moments onto j_z <= 1 (pads zeroed)
-template <int P>
-__global__ void m2l_reduce_moments_h(int64_t nrows, const float *__restrict__ Ms, int ncp, float *__restrict__ Mr, int ncpr,
+template <int P, class T>
+__global__ void m2l_reduce_moments_h(int64_t nrows, const T *__restrict__ Ms, int ncp, T *__restrict__ Mr, int ncpr,
                                      const int *drows)
 {
     if (drows) nrows = *drows;
     for (int64_t w = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; w < nrows; w += (int64_t)gridDim.x * blockDim.x) {
         M2LGenH<P>::reduce_moments(Ms + w * ncp, Mr + w * ncpr);
-        for (int k = M2LGenH<P>::NC; k < ncpr; ++k) Mr[w * ncpr + k] = 0.f;
+        for (int k = M2LGenH<P>::NC; k < ncpr; ++k) Mr[w * ncpr + k] = T(0);
     }
 }
 
 // per cell and class: the full local expansion from its n_z <= 1 coefficients (pads zeroed)
-template <int P>
-__global__ void m2l_complete_locals_h(int64_t nrows, const float *__restrict__ Lr, int ncpr, float *__restrict__ L, int ncp,
+template <int P, class T>
+__global__ void m2l_complete_locals_h(int64_t nrows, const T *__restrict__ Lr, int ncpr, T *__restrict__ L, int ncp,
                                       const int *drows)
 {
     if (drows) nrows = *drows;
     constexpr int NC = M2LGen<P>::NC;
     for (int64_t w = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; w < nrows; w += (int64_t)gridDim.x * blockDim.x) {
         M2LGenH<P>::complete_locals(Lr + w * ncpr, L + w * ncp);
-        for (int k = NC; k < ncp; ++k) L[w * ncp + k] = 0.f;
+        for (int k = NC; k < ncp; ++k) L[w * ncp + k] = T(0);
     }
 }
 
@@ -472,9 +474,122 @@ __global__ void __launch_bounds__(128) m2l_directed_h(TreeView t, const uint32_t
     if (class_ctr && lane == 0 && my_sc) atomicAdd(class_ctr, my_sc);
 }
 
+// ------------------------------------------------------------------ float64, fixed order P <= 6
+// The float64 pipe (2 lanes per clock and SM) is all that counts here: the operations per cell pair, and that
+// every lane of a warp holds a pair.  A warp takes `chunk` blocks, counts their pairs and deals them to its
+// lanes densely, 32 at a time; a lane builds D once and adds both sides of both classes to the cells with
+// float64 atomics (which L2 adds, not the SM).  The contractions are the generated ones, with the harmonic set
+// for the Wendland kernel: 966 instead of 1680 multiply-adds per pair and class at p = 6 without the potential.
+// A tree with fewer blocks than warps hands out one block at a time, and the sides and classes of a pair to
+// `split` different warps (each builds D again), since a warp's round of 32 pairs lasts as long as all its
+// float64 operations.  Classes are skipped as in m2l_blocks_f32.
+// Lanes laid out 4 rows x 8 columns (half of them idle), run-time loops and the full set took 32.4 ms for
+// the 1.06e6 cell pairs of a 100,003-particle sphere's kick pair at p = 6; this form takes 6.2 ms.
+template <class G, bool MASKED, bool POT>
+__global__ void __launch_bounds__(128) m2l_pairs_f64(TreeView t, const M2LBlock *__restrict__ blocks, int64_t nb,
+                                                     const unsigned long long *dnb, const double *__restrict__ Ms,
+                                                     double *L, int ncp, double eps_over_L, int plummer,
+                                                     const DevEval *de, const Geom *gp, double eps,
+                                                     const uint32_t *__restrict__ fpre)
+{
+    if (de) {   // batched path: classes, count and root cube on the device
+        if ((de->masked != 0) != MASKED) return;
+        nb = (int64_t)*dnb;
+        if (plummer) eps_over_L = ldexp(eps, -gp->log2L);
+    }
+    constexpr int NC = G::NC, ND = G::ND, NIT = MASKED ? 4 : 2;
+    __shared__ M2LBlock s_blk[4][32];
+    __shared__ int s_inc[4][32];
+    const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
+    const int64_t wid = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+    const int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
+    const int chunk = (int)min((int64_t)32, (nb + nw - 1) / nw);
+    const int64_t nchunk = chunk > 0 ? (nb + chunk - 1) / chunk : 0;
+    int split = 1;
+    while (split < NIT && nchunk * split * 2 <= nw) split *= 2;
+    for (int64_t w = wid; w < nchunk * split; w += nw) {
+        const int64_t b0 = (w / split) * chunk;
+        const int part = (int)(w % split);
+        __syncwarp();
+        int cnt = 0;
+        if (lane < chunk && b0 + lane < nb) {
+            const M2LBlock b = blocks[b0 + lane];
+            s_blk[wib][lane] = b;
+            cnt = __popcll(b.mask);
+        }
+        int inc = cnt;
+#pragma unroll
+        for (int d = 1; d < 32; d <<= 1) {
+            const int u = __shfl_up_sync(0xffffffffu, inc, d);
+            if (lane >= d) inc += u;
+        }
+        s_inc[wib][lane] = inc;
+        const int total = __shfl_sync(0xffffffffu, inc, 31);
+        __syncwarp();
+        for (int q0 = 0; q0 < total; q0 += 32) {
+            const int q = q0 + lane;
+            const bool active = q < total;
+            int x = 0, y = 0, lx = 0, ly = 0;
+            if (active) {
+                int s = 0;   // the block of pair q: the first with inc > q
+#pragma unroll
+                for (int b = 16; b >= 1; b >>= 1)
+                    if (s_inc[wib][s + b - 1] <= q) s += b;
+                const M2LBlock blk = s_blk[wib][s];
+                unsigned long long m = blk.mask;
+                for (int r = q - (s ? s_inc[wib][s - 1] : 0); r > 0; --r) m &= m - 1;
+                const int bit = __ffsll((long long)m) - 1;
+                const BlockGeom bg = block_geom(t, blk);
+                x = bg.baseA + (bit >> 3);
+                y = bg.baseB + (bit & 7);
+                lx = bg.lx;
+                ly = bg.ly;
+            }
+            unsigned need = 0xfu;   // bit cls: side x needs class cls; bit 2 + cls: side y does
+            if (MASKED && fpre) {
+                int fx = 0, sx = 0, fy = 0, sy = 0;
+                if (active) {
+                    const int ax = t.first[x], ay = t.first[y];
+                    fx = (int)(fpre[ax + t.count[x]] - fpre[ax]);
+                    sx = t.count[x] - fx;
+                    fy = (int)(fpre[ay + t.count[y]] - fpre[ay]);
+                    sy = t.count[y] - fy;
+                }
+                need = (__any_sync(0xffffffffu, sx > 0) ? 1u : 0u) | (__any_sync(0xffffffffu, fx > 0 && sy > 0) ? 2u : 0u) |
+                       (__any_sync(0xffffffffu, sy > 0) ? 4u : 0u) | (__any_sync(0xffffffffu, fy > 0 && sx > 0) ? 8u : 0u);
+            }
+            if (!active) continue;
+            const double rho = ldexp(1.0, lx - ly);
+            const double soft = plummer ? ldexp(eps_over_L, lx) : 0.0;   // eps / s_x
+            double dx, dy, dz, D[ND];
+            pair_offset<double>(t, x, y, lx, ly, dx, dy, dz);
+            G::dt(dx, dy, dz, soft * soft, D);
+            // side x with sources y, then side y with sources x as the same contraction at rho = -1 (the flush
+            // applies (-1)^|n| rho^(|n|+1)); one copy of the generated code for all of them
+#pragma unroll 1
+            for (int it = part; it < NIT; it += split) {
+                const int cls = it >> 1, side = it & 1;
+                if (!(need & ((side ? 4u : 1u) << cls))) continue;
+                double Lc[NC];
+                const double *src = Ms + ((size_t)(side ? x : y) * 2 + cls) * ncp;
+                if (POT) G::side_a(D, src, side ? -1.0 : rho, Lc);
+                else G::side_a_forces(D, src, side ? -1.0 : rho, Lc);
+                double *dst = L + ((size_t)(side ? y : x) * 2 + cls) * ncp;
+                double sc = side ? rho : 1.0;
+                const double step = side ? -rho : 1.0;
+#pragma unroll
+                for (int k = 0; k < NC; ++k) {
+                    if (k > 0 && order_in(G::HARMONIC, k) != order_in(G::HARMONIC, k - 1)) sc *= step;
+                    if (POT || k > 0) atomicAdd(dst + k, Lc[k] * sc);
+                }
+            }
+        }
+    }
+}
+
 // ------------------------------------------------------------------ generic (p <= 8, float or double)
 // Same block layout; each active lane evaluates its pair with run-time loops and adds both sides
-// directly to global memory.  Used by the float64 path and by float32 for p > 6.
+// directly to global memory.  Used for 6 < p <= 8.
 template <class T>
 __device__ __forceinline__ void dtensor_generic(int p, T dx, T dy, T dz, T soft2, T *D)
 {
@@ -507,14 +622,8 @@ __device__ __forceinline__ void dtensor_generic(int p, T dx, T dy, T dz, T soft2
 template <class T, bool MASKED>
 __global__ void m2l_blocks_generic(TreeView t, const M2LBlock *__restrict__ blocks, int64_t nblocks,
                                    const T *__restrict__ Ms, T *L, int p, int nc, int ncp, double eps_over_L,
-                                   int plummer, const unsigned long long *dnb = nullptr, const DevEval *de = nullptr,
-                                   const Geom *gp = nullptr, double eps = 0.0)
+                                   int plummer)
 {
-    if (dnb) {   // batched path: counts, classes and root cube on the device
-        if ((de->masked != 0) != MASKED) return;
-        nblocks = (int64_t)*dnb;
-        if (plummer) eps_over_L = ldexp(eps, -gp->log2L);
-    }
     const int lane = threadIdx.x & 31;
     const int64_t wid = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     const int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;

@@ -242,9 +242,9 @@ tg_status launch_m2l_f32_dev(tg_ctx *c, const TreeView &t, const DevEval *de, co
                              int ncp, int cap_cells, size_t cap_src, const uint32_t *fpre);
 tg_status launch_m2l_f64_dev(tg_ctx *c, const TreeView &t, const DevEval *de, const Geom *gp, const M2LBlock *blocks,
                              const unsigned long long *dnb, int64_t cap_blocks, const double *Ms, double *L, int p,
-                             int ncp);
+                             int ncp, const uint32_t *fpre);
 tg_status launch_m2l_f64(tg_ctx *c, const TreeView &t, const M2LBlock *blocks, int64_t nblocks, const double *Ms,
-                         double *L, int p, int nc, int ncp, bool masked);
+                         double *L, int p, int nc, int ncp, bool masked, bool pot, const uint32_t *fpre);
 // ---- p2p.cu: mutual P2P of all leaf pairs (distinct pairs and self pairs) into acc4.
 tg_status launch_p2p_f32(tg_ctx *c, const TreeView &t, const uint2 *pairs, int64_t npairs, const uint2 *self_pairs,
                          int64_t nself, const float4 *pf, const int32_t *nslow, bool pot, double *acc4);
@@ -300,8 +300,6 @@ struct BatchCaps {
 // counters of eval_finish_dev.  No host synchronisation, so it can be captured in a CUDA graph.
 tg_status fmm_eval_dev(tg_ctx *c, DevEval *de, const BatchCaps &cap, const double *xin, const double *min,
                        const uint8_t *fin, double *acc, unsigned long long *stats);
-// zero rows[0] rows of `width` floats (device row count)
-__global__ void zero_rows_f32(float *p, const int *rows, int width);
 // constant part of the acceptance thresholds into device memory (before a capture; synchronising)
 tg_status mac_params_upload(tg_ctx *c);
 

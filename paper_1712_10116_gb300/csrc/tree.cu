@@ -396,13 +396,6 @@ tg_status root_cube(tg_ctx *c, int n, const double *pos, int64_t stride, const i
     return cuda_check(c, cudaGetLastError(), "root cube");
 }
 
-// zero rows[0] rows of `width` floats (device row count)
-__global__ void zero_rows_f32(float *p, const int *rows, int width)
-{
-    const int64_t n = (int64_t)*rows * width;
-    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) p[i] = 0.f;
-}
-
 // ------------------------------------------------------------------ input check
 __global__ void count_nonfinite(const double *pos, int64_t stride, const int64_t *sub, int64_t n, const double *mass,
                                 unsigned long long *bad)
