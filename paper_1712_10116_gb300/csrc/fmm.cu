@@ -898,16 +898,7 @@ static tg_status run_walk(tg_ctx *c, const TreeView &t, int64_t *n_blocks, int64
                           int64_t *n_self)
 {
     tg_status st;
-    int log2L = 0;
-    {
-        const Geom *dg = static_cast<const Geom *>(c->buf[B_GEOM].p);
-        cudaMemcpyAsync(c->h_pinned + 32, &dg->log2L, sizeof(int), cudaMemcpyDeviceToHost, c->stream);
-        cudaError_t e = stream_sync(c);
-        if (e != cudaSuccess) return cuda_check(c, e, "walk setup");
-        log2L = *reinterpret_cast<int *>(c->h_pinned + 32);
-    }
-    const MacParams mp = make_mac_params(c->prm, log2L);
-    c->walk_log2L = log2L;
+    const MacParams mp = make_mac_params(c->prm, c->walk_log2L);
     // capacities from the largest list sizes per cell seen so far (plus a margin), so that a walk is
     // normally run once
     size_t cap_front = (size_t)(t.ncell * c->walk_front_per_cell * 1.25) + 1024,
@@ -1290,7 +1281,7 @@ static tg_status fmm_eval_dev_t(tg_ctx *c, DevEval *de, const BatchCaps &cap, co
         mac_params_dev<<<1, 32, 0, c->stream>>>(d_geom, c->prm.eps, mpd);
     }
     if ((st = keys_sort_gather(c, cap.n, xin, cap.n, nullptr, min, fin, d_geom, de))) return st;
-    if ((st = build_octree_dev(c, de, cap.cells, cap.levels))) return st;
+    if ((st = build_octree_dev(c, de, cap.n, cap.cells, cap.levels))) return st;
     TreeView t = tree_view(c, cap.n, cap.cells);
     t.d_ncell = &de->ncell;
 

@@ -702,7 +702,7 @@ static tg_status hold_presize(tg_ctx *c, const Sched &s, const BatchCaps &cap, c
         {B_PERM2, 4ull * n}, {B_NSLOW, 4ull * C}, {B_PF, 4 * tsz * n}, {B_LEAF_OF, 4ull * n},
         {B_C_LEVEL, 1ull * C}, {B_C_X, 4ull * C}, {B_C_Y, 4ull * C}, {B_C_Z, 4ull * C}, {B_C_FIRST, 4ull * C},
         {B_C_COUNT, 4ull * C}, {B_C_CHILD, 4ull * C}, {B_C_PARENT, 4ull * C}, {B_C_NCHILD, 1ull * C},
-        {B_C_TMP0, 4ull * C}, {B_C_TMP1, 4ull * C},
+        {B_C_CEND, 4ull * C}, {B_C_LVL, 2ull * n}, {B_C_CNT, 4 * oct_count_words(n)},
         {B_MOM, tsz * rows * ncp}, {B_MOMF, tsz * rows * ncp}, {B_MOM01, 8 * rows * 4}, {B_LOC, tsz * rows * ncp},
         {B_ACC, 32ull * n}, {B_MOMH, tsz * rows * ncpr}, {B_LOCH, tsz * rows * ncpr},
         {B_FRONT0, 8 * cap.front}, {B_FRONT1, 8 * cap.front}, {B_M2L, 16 * cap.blocks}, {B_P2P, 8 * cap.p2p},

@@ -2,6 +2,7 @@
 #pragma once
 
 #include <cuda_runtime.h>
+#include <algorithm>
 #include <cstdint>
 #include <cstdio>
 #include <string>
@@ -53,10 +54,8 @@ struct DevEval {
     int hist_items;         // digit histogram entries: kSortBins * sort_blocks
     int ncell;              // cells of the tree
     int nlev;               // levels of the tree
-    int lvl_m;              // cells of the level being split (octree build)
     int rows;               // 2 * ncell (expansion rows, both classes)
     int np1;                // n + 1 (prefix sum of the fast flags, with its total)
-    uint32_t lvl_total;     // children emitted by the level being split (scan total)
     uint32_t overflow;      // bit 0: cells, bit 1: levels, bit 2: walk lists; the step must be redone
     int level_begin[kMaxLevel + 3];   // first cell of each level; [nlev] = ncell
 };
@@ -147,7 +146,7 @@ enum Slot {
     B_XS, B_YS, B_ZS, B_MS, B_FS, B_PF, B_LEAF_OF,
     B_XS2, B_YS2, B_ZS2, B_MS2, B_FS2, B_PERM2, B_NSLOW,
     B_C_LEVEL, B_C_X, B_C_Y, B_C_Z, B_C_FIRST, B_C_COUNT, B_C_CHILD, B_C_PARENT, B_C_NCHILD,
-    B_C_TMP0, B_C_TMP1, B_C_RAD, B_C_RADF,
+    B_C_CEND, B_C_LVL, B_C_CNT, B_OCT, B_C_RAD, B_C_RADF,
     B_MOM, B_MOMF, B_MOM01, B_LOC, B_ACC, B_MOMH, B_LOCH,
     B_FRONT0, B_FRONT1, B_M2L, B_P2P, B_WALK_CNT,
     B_SUB_ACC, B_HHS_AOLD, B_HHS_ACUR, B_HHS_ATOT, B_TRAD_ACC, B_TRAD_END, B_HHS_DT, B_HHS_RUNG, B_HHS_IDX, B_HHS_FLAG,
@@ -192,11 +191,15 @@ tg_status root_cube(tg_ctx *c, int n, const double *pos, int64_t stride, const i
 // slots: B_KEYS0 (sorted keys), B_VALS0 (perm: sorted -> input index q), B_XS.. B_FS.
 tg_status keys_sort_gather(tg_ctx *c, int n, const double *pos, int64_t stride, const int64_t *sub,
                            const double *mass, const uint8_t *fast, const Geom *d_geom, const DevEval *de = nullptr);
-// Octree from the sorted keys; fills the cell slots and c->level_begin.  Returns ncell.
-tg_status build_octree(tg_ctx *c, int n, int *ncell_out);
 TreeView tree_view(tg_ctx *c, int n, int ncell);
-// The same octree with its sizes on the device (de): `cap` cells at most, `levels` levels issued.
-tg_status build_octree_dev(tg_ctx *c, DevEval *de, int cap, int levels);
+
+// ---- octree.cu
+// Octree from the sorted keys; fills the cell slots, c->level_begin and c->walk_log2L.  Returns ncell.
+tg_status build_octree(tg_ctx *c, int n, int *ncell_out);
+// The same octree with its sizes on the device (de): at most cap_n particles and `cap` cells, levels 0 .. `levels`.
+tg_status build_octree_dev(tg_ctx *c, DevEval *de, int cap_n, int cap, int levels);
+// words of the per-tile cell counts of n particles (B_C_CNT)
+size_t oct_count_words(int n);
 
 // Expansion kernels for orders above the fixed tables (TG_PMAX < p <= kPHigh), high_order.cu.
 constexpr int kPHigh = 20;

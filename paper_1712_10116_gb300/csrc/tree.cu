@@ -1,5 +1,5 @@
-// tree.cu -- root cube, Morton keys, stable LSD radix sort, gather and level-synchronous
-// octree build (Sec. 2.3 of Zhu 2017: octree with leaf size n_crit, built for every call).
+// tree.cu -- root cube, Morton keys, stable LSD radix sort and gather (Sec. 2.3 of Zhu 2017: octree with leaf
+// size n_crit, built for every call; the octree itself is octree.cu).
 //
 // Keys: 21 bits per axis, x the most significant bit of each 3-bit group, so a cell at level l
 // is the run of sorted keys sharing the top 3l bits.  The sort orders (key, input index), so ties
@@ -73,46 +73,6 @@ tg_status ensure(tg_ctx *c, int slot, size_t bytes, void **out)
     }
     *out = b.p;
     return TG_OK;
-}
-
-// grow keeping the first `keep` bytes
-static tg_status ensure_keep(tg_ctx *c, int slot, size_t bytes, size_t keep, void **out)
-{
-    Buf &b = c->buf[slot];
-    if (b.bytes >= bytes) {
-        *out = b.p;
-        return TG_OK;
-    }
-    size_t nb = bytes + bytes / 2 + 256;
-    if (c->capturing)
-        return set_err(c, TG_ERR_CAPACITY, "scratch slot %d would grow to %zu bytes inside a graph capture", slot, nb);
-    if (tg_status inj = injected_alloc_failure(c, nb, slot)) return inj;
-    c->alloc_epoch += 1;
-    void *np = nullptr;
-    cudaError_t e = cudaMalloc(&np, nb);
-    if (e != cudaSuccess) {
-        cudaGetLastError();
-        return set_err(c, TG_ERR_OOM, "cudaMalloc(%zu) for scratch slot %d failed", nb, slot);
-    }
-    if (b.p) {
-        if (keep) cudaMemcpyAsync(np, b.p, keep, cudaMemcpyDeviceToDevice, c->stream);
-        e = stream_sync(c);
-        if (e != cudaSuccess) return cuda_check(c, e, "sync before regrow");
-        cudaFree(b.p);
-    }
-    b.p = np;
-    b.bytes = nb;
-    *out = np;
-    return TG_OK;
-}
-
-template <class T>
-static tg_status ensure_keep_t(tg_ctx *c, int slot, size_t count, size_t keep_count, T **out)
-{
-    void *p = nullptr;
-    tg_status s = ensure_keep(c, slot, count * sizeof(T) + 16, keep_count * sizeof(T), &p);
-    *out = static_cast<T *>(p);
-    return s;
 }
 
 // ------------------------------------------------------------------ live kernel timing
@@ -639,279 +599,6 @@ tg_status keys_sort_gather(tg_ctx *c, int n, const double *pos, int64_t stride, 
                                                                dn);
     }
     return cuda_check(c, cudaGetLastError(), "keys/sort/gather");
-}
-
-// ------------------------------------------------------------------ octree
-__device__ __forceinline__ int key_digit(uint64_t key, int lvl) { return (int)((key >> (3 * (kMaxLevel - lvl))) & 7u); }
-
-// first index in [s, e) whose digit at level lvl is >= d (digits are sorted within a cell)
-__device__ __forceinline__ int digit_lower_bound(const uint64_t *keys, int s, int e, int lvl, int d)
-{
-    while (s < e) {
-        int m = (s + e) >> 1;
-        if (key_digit(keys[m], lvl) < d) s = m + 1;
-        else e = m;
-    }
-    return s;
-}
-
-// Child boundaries of a cell that splits: warp per cell, lane d (1..7) finds the first particle whose
-// digit at the child level is >= d; lane 0 holds the cell start and lanes 8..31 its end, so that child
-// d (lane d < 8) spans [b_d, b_{d+1}).  The seven binary searches run side by side.
-__device__ __forceinline__ int child_bound(const uint64_t *keys, int s, int e, int l, int lane)
-{
-    if (lane == 0) return s;
-    if (lane >= 8) return e;
-    return digit_lower_bound(keys, s, e, l, lane);
-}
-
-// Children of cell cidx (the t-th cell of its level): count (cnt[t]) and emission at le + off[t].
-// The whole warp handles one cell.
-__device__ __forceinline__ void oct_count_cell(const uint64_t *keys, int cidx, int t, const uint8_t *level,
-                                               const int32_t *first, const int32_t *count, int n_crit, int max_level,
-                                               uint32_t *cnt, int lane)
-{
-    if (count[cidx] <= n_crit || level[cidx] >= max_level) {
-        if (lane == 0) cnt[t] = 0;
-        return;
-    }
-    const int l = level[cidx] + 1, s = first[cidx], e = s + count[cidx];
-    const int b = child_bound(keys, s, e, l, lane);
-    const int bn = __shfl_down_sync(0xffffffffu, b, 1);
-    const unsigned m = __ballot_sync(0xffffffffu, lane < 8 && bn > b);
-    if (lane == 0) cnt[t] = __popc(m);
-}
-
-__device__ __forceinline__ void oct_emit_cell(const uint64_t *keys, int le, int cidx, int t, uint8_t *level,
-                                              uint32_t *cx, uint32_t *cy, uint32_t *cz, int32_t *first, int32_t *count,
-                                              int32_t *child_first, int32_t *parent, uint8_t *nchild,
-                                              const uint32_t *off, const uint32_t *cnt, int lane)
-{
-    const int nch = cnt[t];
-    if (nch == 0) {
-        if (lane == 0) {
-            nchild[cidx] = 0;
-            child_first[cidx] = -1;
-        }
-        return;
-    }
-    const int base = le + (int)off[t];
-    const int l = level[cidx] + 1, s = first[cidx], e = s + count[cidx];
-    const uint32_t px = cx[cidx], py = cy[cidx], pz = cz[cidx];
-    const int b = child_bound(keys, s, e, l, lane);
-    const int bn = __shfl_down_sync(0xffffffffu, b, 1);
-    const bool nonempty = lane < 8 && bn > b;
-    const unsigned m = __ballot_sync(0xffffffffu, nonempty);
-    if (nonempty) {
-        const int digit = lane, ch = base + __popc(m & ((1u << lane) - 1u));
-        level[ch] = (uint8_t)l;
-        cx[ch] = 2u * px + ((digit >> 2) & 1);
-        cy[ch] = 2u * py + ((digit >> 1) & 1);
-        cz[ch] = 2u * pz + (digit & 1);
-        first[ch] = b;
-        count[ch] = bn - b;
-        parent[ch] = cidx;
-        nchild[ch] = 0;
-        child_first[ch] = -1;
-    }
-    if (lane == 0) {
-        nchild[cidx] = (uint8_t)nch;
-        child_first[cidx] = base;
-    }
-}
-
-__global__ void oct_count(const uint64_t *keys, int lb, int le, const uint8_t *level, const int32_t *first,
-                          const int32_t *count, int n_crit, int max_level, uint32_t *cnt)
-{
-    const int t = (int)(((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5), lane = threadIdx.x & 31;
-    const int cidx = lb + t;
-    if (cidx >= le) return;   // whole warp
-    oct_count_cell(keys, cidx, t, level, first, count, n_crit, max_level, cnt, lane);
-}
-__global__ void oct_emit(const uint64_t *keys, int lb, int le, uint8_t *level, uint32_t *cx, uint32_t *cy,
-                         uint32_t *cz, int32_t *first, int32_t *count, int32_t *child_first, int32_t *parent,
-                         uint8_t *nchild, const uint32_t *off, const uint32_t *cnt)
-{
-    const int t = (int)(((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5), lane = threadIdx.x & 31;
-    const int cidx = lb + t;
-    if (cidx >= le) return;   // whole warp
-    oct_emit_cell(keys, le, cidx, t, level, cx, cy, cz, first, count, child_first, parent, nchild, off, cnt, lane);
-}
-__global__ void oct_root(int n, uint8_t *level, uint32_t *cx, uint32_t *cy, uint32_t *cz, int32_t *first,
-                         int32_t *count, int32_t *child_first, int32_t *parent, uint8_t *nchild)
-{
-    level[0] = 0;
-    cx[0] = cy[0] = cz[0] = 0;
-    first[0] = 0;
-    count[0] = n;
-    child_first[0] = -1;
-    parent[0] = -1;
-    nchild[0] = 0;
-}
-
-tg_status build_octree(tg_ctx *c, int n, int *ncell_out)
-{
-    tg_status st;
-    const uint64_t *keys = static_cast<const uint64_t *>(c->buf[B_KEYS0].p);
-    int cap = 1024 + n / 4;
-    uint8_t *level, *nchild;
-    uint32_t *cx, *cy, *cz, *cnt, *off;
-    int32_t *first, *count, *child_first, *parent;
-    auto grow = [&](int need, int keep) -> tg_status {
-        tg_status s;
-        if ((s = ensure_keep_t(c, B_C_LEVEL, need, keep, &level)) || (s = ensure_keep_t(c, B_C_X, need, keep, &cx)) ||
-            (s = ensure_keep_t(c, B_C_Y, need, keep, &cy)) || (s = ensure_keep_t(c, B_C_Z, need, keep, &cz)) ||
-            (s = ensure_keep_t(c, B_C_FIRST, need, keep, &first)) ||
-            (s = ensure_keep_t(c, B_C_COUNT, need, keep, &count)) ||
-            (s = ensure_keep_t(c, B_C_CHILD, need, keep, &child_first)) ||
-            (s = ensure_keep_t(c, B_C_PARENT, need, keep, &parent)) ||
-            (s = ensure_keep_t(c, B_C_NCHILD, need, keep, &nchild)))
-            return s;
-        return TG_OK;
-    };
-    if ((st = grow(cap, 0))) return st;
-    {
-        ProfScope ps_(c, TG_K_TREE);
-        oct_root<<<1, 1, 0, c->stream>>>(n, level, cx, cy, cz, first, count, child_first, parent, nchild);
-    }
-    c->level_begin.assign(1, 0);
-    int lb = 0, le = 1;
-    uint32_t *h_total = reinterpret_cast<uint32_t *>(c->h_pinned);
-    uint32_t *d_total = reinterpret_cast<uint32_t *>(c->d_counters + 8);
-    for (int lvl = 0; lvl < c->prm.max_level && le > lb; ++lvl) {
-        const int m = le - lb;
-        if ((st = ensure_t(c, B_C_TMP0, m, &cnt)) || (st = ensure_t(c, B_C_TMP1, m, &off))) return st;
-        {
-            ProfScope ps_(c, TG_K_TREE);
-            oct_count<<<(int)(((int64_t)m * 32 + 255) / 256), 256, 0, c->stream>>>(keys, lb, le, level, first, count, c->prm.n_crit,
-                                                             c->prm.max_level, cnt);
-        }
-        if ((st = exclusive_scan_u32(c, cnt, off, m, d_total, nullptr))) return st;
-        cudaMemcpyAsync(h_total, d_total, sizeof(uint32_t), cudaMemcpyDeviceToHost, c->stream);
-        cudaError_t e = stream_sync(c);
-        if (e != cudaSuccess) return cuda_check(c, e, "octree level");
-        const int total = (int)*h_total;
-        if (le + total > cap) {
-            int ncap = le + total + (le + total) / 2 + 1024;
-            if ((st = grow(ncap, le))) return st;
-            cap = ncap;
-        }
-        {
-            ProfScope ps_(c, TG_K_TREE);
-            oct_emit<<<(int)(((int64_t)m * 32 + 255) / 256), 256, 0, c->stream>>>(keys, lb, le, level, cx, cy, cz, first, count, child_first,
-                                                            parent, nchild, off, cnt);
-        }
-        c->level_begin.push_back(le);
-        lb = le;
-        le = le + total;
-    }
-    if (c->level_begin.back() != le) c->level_begin.push_back(le);
-    *ncell_out = le;
-    return cuda_check(c, cudaGetLastError(), "octree");
-}
-
-// ------------------------------------------------------------------ octree, sizes on the device
-// The batched path builds the same tree level by level, but the level ranges, the cell count and
-// the depth stay on the device (DevEval): launches are sized for the capacity, warps stride over the
-// cells of their level, and levels past the tree's depth find no cells.  A level whose children
-// would pass the cell capacity, or a tree deeper than the levels issued, sets an overflow bit; the
-// step is then redone with larger buffers.
-__global__ void oct_root_dev(DevEval *de, uint8_t *level, uint32_t *cx, uint32_t *cy, uint32_t *cz, int32_t *first,
-                             int32_t *count, int32_t *child_first, int32_t *parent, uint8_t *nchild)
-{
-    level[0] = 0;
-    cx[0] = cy[0] = cz[0] = 0;
-    first[0] = 0;
-    count[0] = de->n;
-    child_first[0] = -1;
-    parent[0] = -1;
-    nchild[0] = 0;
-    de->level_begin[0] = 0;
-    de->level_begin[1] = 1;
-    de->nlev = 1;
-    de->ncell = 1;
-    de->rows = 2;
-    de->lvl_m = 1;
-}
-
-__global__ void oct_count_dev(const uint64_t *keys, const DevEval *de, int lvl, const uint8_t *level,
-                              const int32_t *first, const int32_t *count, int n_crit, int max_level, uint32_t *cnt)
-{
-    if (lvl >= de->nlev) return;
-    const int lb = de->level_begin[lvl], m = de->level_begin[lvl + 1] - lb;
-    const int lane = threadIdx.x & 31, nw = (int)((gridDim.x * blockDim.x) >> 5);
-    for (int t = (int)((blockIdx.x * blockDim.x + threadIdx.x) >> 5); t < m; t += nw)
-        oct_count_cell(keys, lb + t, t, level, first, count, n_crit, max_level, cnt, lane);
-}
-
-__global__ void oct_emit_dev(const uint64_t *keys, const DevEval *de, int lvl, int cap, uint8_t *level, uint32_t *cx,
-                             uint32_t *cy, uint32_t *cz, int32_t *first, int32_t *count, int32_t *child_first,
-                             int32_t *parent, uint8_t *nchild, const uint32_t *off, const uint32_t *cnt)
-{
-    if (lvl >= de->nlev) return;
-    const int lb = de->level_begin[lvl], le = de->level_begin[lvl + 1], m = le - lb;
-    if ((int64_t)le + de->lvl_total > cap) return;   // over capacity: oct_finish_dev flags it
-    const int lane = threadIdx.x & 31, nw = (int)((gridDim.x * blockDim.x) >> 5);
-    for (int t = (int)((blockIdx.x * blockDim.x + threadIdx.x) >> 5); t < m; t += nw)
-        oct_emit_cell(keys, le, lb + t, t, level, cx, cy, cz, first, count, child_first, parent, nchild, off, cnt, lane);
-}
-
-__global__ void oct_finish_dev(DevEval *de, int lvl, int cap, int last_issued, int max_level)
-{
-    if (lvl >= de->nlev) {
-        de->lvl_m = 0;
-        return;
-    }
-    const int le = de->level_begin[lvl + 1];
-    int total = (int)de->lvl_total;
-    if ((int64_t)le + total > cap) {
-        de->overflow |= 1u;
-        total = 0;
-    }
-    if (total > 0) {
-        de->level_begin[lvl + 2] = le + total;
-        de->nlev = lvl + 2;
-        de->ncell = le + total;
-        de->rows = 2 * (le + total);
-        if (last_issued && lvl + 1 < max_level) de->overflow |= 2u;   // the tree goes deeper than issued
-    }
-    de->lvl_m = total;
-}
-
-tg_status build_octree_dev(tg_ctx *c, DevEval *de, int cap, int levels)
-{
-    tg_status st;
-    const uint64_t *keys = static_cast<const uint64_t *>(c->buf[B_KEYS0].p);
-    uint8_t *level, *nchild;
-    uint32_t *cx, *cy, *cz, *cnt, *off;
-    int32_t *first, *count, *child_first, *parent;
-    if ((st = ensure_t(c, B_C_LEVEL, cap, &level)) || (st = ensure_t(c, B_C_X, cap, &cx)) ||
-        (st = ensure_t(c, B_C_Y, cap, &cy)) || (st = ensure_t(c, B_C_Z, cap, &cz)) ||
-        (st = ensure_t(c, B_C_FIRST, cap, &first)) || (st = ensure_t(c, B_C_COUNT, cap, &count)) ||
-        (st = ensure_t(c, B_C_CHILD, cap, &child_first)) || (st = ensure_t(c, B_C_PARENT, cap, &parent)) ||
-        (st = ensure_t(c, B_C_NCHILD, cap, &nchild)) || (st = ensure_t(c, B_C_TMP0, cap, &cnt)) ||
-        (st = ensure_t(c, B_C_TMP1, cap, &off)))
-        return st;
-    {
-        ProfScope ps_(c, TG_K_TREE);
-        oct_root_dev<<<1, 1, 0, c->stream>>>(de, level, cx, cy, cz, first, count, child_first, parent, nchild);
-    }
-    const int grid = c->num_sms * 8;
-    for (int lvl = 0; lvl < levels; ++lvl) {
-        {
-            ProfScope ps_(c, TG_K_TREE);
-            oct_count_dev<<<grid, 256, 0, c->stream>>>(keys, de, lvl, level, first, count, c->prm.n_crit,
-                                                       c->prm.max_level, cnt);
-        }
-        if ((st = exclusive_scan_u32(c, cnt, off, cap, &de->lvl_total, &de->lvl_m))) return st;
-        {
-            ProfScope ps_(c, TG_K_TREE);
-            oct_emit_dev<<<grid, 256, 0, c->stream>>>(keys, de, lvl, cap, level, cx, cy, cz, first, count, child_first,
-                                                      parent, nchild, off, cnt);
-            oct_finish_dev<<<1, 1, 0, c->stream>>>(de, lvl, cap, lvl == levels - 1, c->prm.max_level);
-        }
-    }
-    return cuda_check(c, cudaGetLastError(), "octree (device sizes)");
 }
 
 TreeView tree_view(tg_ctx *c, int n, int ncell)
