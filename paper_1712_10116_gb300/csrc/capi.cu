@@ -194,12 +194,12 @@ tg_status tg_build_tree(tg_ctx *c, int64_t n, const double *pos)
     if (n <= 0 || n > INT32_MAX / 4 || !check_device_ptr(pos))
         return set_err(c, TG_ERR_ARG, "tg_build_tree: need n > 0 and a device pointer");
     Geom *g;
-    if ((st = ensure_t(c, B_GEOM, 1, &g)) || (st = root_cube(c, (int)n, pos, n, nullptr, g))) return st;
+    if ((st = ensure_t(c, B_GEOM, 1, &g))) return st;
     // masses are not needed for the tree; gather reads a dummy unit array
     double *ones;
     if ((st = ensure_t(c, B_DIAG_POT, n, &ones))) return st;
     cudaMemsetAsync(ones, 0, sizeof(double) * n, c->stream);
-    if ((st = keys_sort_gather(c, (int)n, pos, n, nullptr, ones, nullptr, g))) return st;
+    if ((st = sort_particles(c, (int)n, pos, n, nullptr, ones, nullptr, g))) return st;
     int ncell = 0;
     if ((st = build_octree(c, (int)n, &ncell))) return st;
     c->last_n = n;

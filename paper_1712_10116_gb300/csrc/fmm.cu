@@ -1122,8 +1122,7 @@ tg_status fmm_eval(tg_ctx *c, int n, const double *pos, int64_t stride, const in
     if (n <= 0) return TG_OK;
     Geom *d_geom;
     if ((st = ensure_t(c, B_GEOM, 1, &d_geom))) return st;
-    if ((st = root_cube(c, n, pos, stride, sub, d_geom))) return st;
-    if ((st = keys_sort_gather(c, n, pos, stride, sub, mass, fast, d_geom))) return st;
+    if ((st = sort_particles(c, n, pos, stride, sub, mass, fast, d_geom))) return st;
     int ncell = 0;
     if ((st = build_octree(c, n, &ncell))) return st;
     TreeView t = tree_view(c, n, ncell);
@@ -1275,12 +1274,11 @@ static tg_status fmm_eval_dev_t(tg_ctx *c, DevEval *de, const BatchCaps &cap, co
     Geom *d_geom;
     MacParams *mpd;
     if ((st = ensure_t(c, B_GEOM, 1, &d_geom)) || (st = ensure_t(c, B_MACP, 1, &mpd))) return st;
-    if ((st = root_cube(c, cap.n, xin, cap.n, nullptr, d_geom, &de->n))) return st;
+    if ((st = sort_particles(c, cap.n, xin, cap.n, nullptr, min, fin, d_geom, de))) return st;
     {
         ProfScope ps_(c, TG_K_WALK);
         mac_params_dev<<<1, 32, 0, c->stream>>>(d_geom, c->prm.eps, mpd);
     }
-    if ((st = keys_sort_gather(c, cap.n, xin, cap.n, nullptr, min, fin, d_geom, de))) return st;
     if ((st = build_octree_dev(c, de, cap.n, cap.cells, cap.levels))) return st;
     TreeView t = tree_view(c, cap.n, cap.cells);
     t.d_ncell = &de->ncell;

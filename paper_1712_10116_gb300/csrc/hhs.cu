@@ -559,8 +559,6 @@ __global__ void hold_frame(const HoldState *h, LevelLayout lv, const double *pos
         de->n = (int)ns;
         de->np1 = (int)ns + 1;
         de->masked = masked;
-        de->sort_blocks = (int)((ns + kSortTileItems - 1) / kSortTileItems);
-        de->hist_items = kSortBins * de->sort_blocks;
     }
     for (int64_t q = tid; q < ns; q += (int64_t)gridDim.x * blockDim.x) {
         const int64_t i = sys[q];
@@ -688,15 +686,14 @@ static tg_status hold_presize(tg_ctx *c, const Sched &s, const BatchCaps &cap, c
     void *p;
     const int n = cap.n, C = cap.cells, p_ = c->prm.p, ncp = (ncoef(p_) + 3) & ~3;
     const size_t rows = (size_t)C * 2;
-    const int nblocks = (n + kSortTileItems - 1) / kSortTileItems;
     const int nh = (p_ + 1) * (p_ + 1), ncpr = (nh + 3) & ~3;
     const int64_t max_units = (int64_t)cap.p2p / 8 + std::min<int64_t>((int64_t)cap.p2p, 32768) + C + 1;   // own_max_units
     const size_t tsz = c->prm.precision == TG_PREC_FP32 ? 4 : 8;   // compute precision
     struct Need { int slot; size_t bytes; };
     const Need needs[] = {
-        {B_GEOM, 64}, {B_PARTIAL, sizeof(double) * 6 * 2 * 152}, {B_KEYS0, 8ull * n}, {B_KEYS1, 8ull * n},
-        {B_VALS0, 4ull * n}, {B_VALS1, 4ull * n}, {B_HIST, 4ull * ((size_t)kSortBins * nblocks + 1)},
-        {B_SCAN_TMP, 4 * std::max(scan_scratch_words(std::max(kSortBins * nblocks, 1)), std::max(scan_scratch_words(C), scan_scratch_words(n + 1)))},
+        {B_GEOM, 64}, {B_KEYS0, 8ull * n}, {B_KEYS1, 8ull * n},
+        {B_VALS0, 4ull * n}, {B_VALS1, 4ull * n},
+        {B_SCAN_TMP, 4 * std::max(scan_scratch_words(C), scan_scratch_words(n + 1))},
         {B_XS, 8ull * n}, {B_YS, 8ull * n}, {B_ZS, 8ull * n}, {B_MS, 8ull * n}, {B_FS, 1ull * n},
         {B_XS2, 8ull * n}, {B_YS2, 8ull * n}, {B_ZS2, 8ull * n}, {B_MS2, 8ull * n}, {B_FS2, 1ull * n},
         {B_PERM2, 4ull * n}, {B_NSLOW, 4ull * C}, {B_PF, 4 * tsz * n}, {B_LEAF_OF, 4ull * n},
@@ -711,11 +708,12 @@ static tg_status hold_presize(tg_ctx *c, const Sched &s, const BatchCaps &cap, c
         {B_OWN_LIST, 8ull * max_units}, {B_OWN_TAG, 8 * cap.p2p}, {B_OWN_PART, 4 * cap.p2p},
         {B_M2L_CNT, 4ull * C}, {B_M2L_OFF, 4ull * C}, {B_M2L_FILL, 4ull * C}, {B_M2L_SRC, 4 * cap.m2l_src},
         {B_FWORDS, 4ull * (n + 1)}, {B_FPRE, 4ull * (n + 1)}, {B_M2L_PART, 16 * cap.blocks}, {B_M2L_PCNT, 16},
-        {B_SCAN_TMP2, 4 * std::max(scan_scratch_words(std::max(kSortBins * nblocks, 1)), std::max(scan_scratch_words(C), scan_scratch_words(n + 1)))},
+        {B_SCAN_TMP2, 4 * std::max(scan_scratch_words(C), scan_scratch_words(n + 1))},
         {B_ACC_P2P, 32ull * n},
         {B_FRAME_X, 24ull * n}, {B_FRAME_M, 8ull * n}, {B_FRAME_F, 1ull * n}, {B_SPLIT_FLAG, 4ull * n},
         {B_SPLIT_PRE, 4ull * n}, {B_HOLD, sizeof(HoldState)}, {B_DEVEVAL, sizeof(DevEval)},
     };
+    if ((st = ensure_sort_scratch(c, n, &p))) return st;
     for (const Need &q : needs)
         if ((st = ensure(c, q.slot, q.bytes + 16, &p))) return st;
     (void)s;
@@ -1000,6 +998,7 @@ tg_status hhs_step_batched(tg_ctx *c)
         if (head.status != 0)
             return fail(set_err(c, TG_ERR_TIMEOUT, "batched step: the device loop stopped after %llu iterations",
                                 head.iterations));
+        if (overflow & 8u) return fail(set_err(c, TG_ERR_TIMEOUT, "batched step: a bounded wait of the particle sort ran out"));
         if (overflow) {
             // restore, grow what ran out, capture again and redo the step
             restore_state(c, s, static_cast<const char *>(c->buf[B_SNAP].p));
@@ -1145,6 +1144,11 @@ tg_status ensemble_step(tg_ctx **cs, int count)
             restore_state(c, sched[i], static_cast<const char *>(c->buf[B_SNAP].p));
             if (!first) first = set_err(c0, TG_ERR_TIMEOUT, "ensemble member %d: the device loop stopped after %llu "
                                                             "iterations", i, head.iterations);
+            continue;
+        }
+        if (overflow & 8u) {
+            restore_state(c, sched[i], static_cast<const char *>(c->buf[B_SNAP].p));
+            if (!first) first = set_err(c0, TG_ERR_TIMEOUT, "ensemble member %d: a bounded wait of the particle sort ran out", i);
             continue;
         }
         if (overflow) {

@@ -100,7 +100,7 @@ __global__ void __launch_bounds__(kOctThreads) oct_levels(const uint64_t *__rest
 // array holds (max_level + 1) entries per 1024 particles.  Levels beyond `levels` or cells beyond `cap` (batched
 // path) are cut off: the tree then ends at the last level that fits, and the step is redone.
 __global__ void __launch_bounds__(1024) oct_scan(int n, const int *dn, int max_level, uint32_t *cnt, DevEval *de, int cap,
-                                                 int levels)
+                                                 int levels, const uint32_t *flag)
 {
     n = dev_or(dn, n);
     const int ntile = n / kOctTile + 1, m = (max_level + 1) * ntile;
@@ -166,7 +166,8 @@ __global__ void __launch_bounds__(1024) oct_scan(int n, const int *dn, int max_l
     de->nlev = nlev;
     de->ncell = ncell;
     de->rows = 2 * ncell;
-    if (over) de->overflow |= over;
+    if (flag) de->overflow = *flag | over;   // host path: the sort's flag travels with the sizes
+    else if (over) de->overflow |= over;
 }
 
 struct OctCells {
@@ -293,7 +294,8 @@ tg_status build_octree(tg_ctx *c, int n, int *ncell_out)
     }
     {
         ProfScope ps_(c, TG_K_TREE);
-        oct_scan<<<1, 1024, 0, c->stream>>>(n, nullptr, c->prm.max_level, cnt, de, INT32_MAX, kMaxLevel + 1);
+        oct_scan<<<1, 1024, 0, c->stream>>>(n, nullptr, c->prm.max_level, cnt, de, INT32_MAX, kMaxLevel + 1,
+                                            sort_scratch(c->buf[B_SORT].p, n).flag);
     }
     // the sizes of the tree, and the root cube's side for the walk, with one wait
     DevEval *h = reinterpret_cast<DevEval *>(c->h_pinned);
@@ -303,6 +305,10 @@ tg_status build_octree(tg_ctx *c, int n, int *ncell_out)
     cudaError_t e = stream_sync(c);
     if (e != cudaSuccess) return cuda_check(c, e, "octree");
     c->walk_log2L = *reinterpret_cast<int *>(c->h_pinned + 32);
+    if (h->overflow & 8u) {
+        cudaMemsetAsync(c->buf[B_SORT].p, 0, 256, c->stream);
+        return set_err(c, TG_ERR_TIMEOUT, "a bounded wait of the particle sort ran out");
+    }
     const int ncell = h->ncell;
     c->level_begin.assign(h->level_begin, h->level_begin + h->nlev + 1);
     OctCells o;
@@ -334,7 +340,7 @@ tg_status build_octree_dev(tg_ctx *c, DevEval *de, int cap_n, int cap, int level
     const int grid = std::min(cap_n / kOctTile + 1, c->num_sms * 8);
     ProfScope ps0_(c, TG_K_TREE), ps1_(c, TG_K_TREE), ps2_(c, TG_K_TREE), ps3_(c, TG_K_TREE);
     oct_levels<<<grid, kOctThreads, 0, c->stream>>>(keys, 0, &de->n, c->prm.n_crit, c->prm.max_level, lvl, cnt);
-    oct_scan<<<1, 1024, 0, c->stream>>>(0, &de->n, c->prm.max_level, cnt, de, cap, levels);
+    oct_scan<<<1, 1024, 0, c->stream>>>(0, &de->n, c->prm.max_level, cnt, de, cap, levels, nullptr);
     oct_cells<<<grid, kOctThreads, 0, c->stream>>>(keys, 0, &de->n, lvl, c->prm.max_level, cnt, de, o);
     oct_finish<<<grid_for(cap, 256, c->num_sms * 8), 256, 0, c->stream>>>(de, o);
     return cuda_check(c, cudaGetLastError(), "octree (device sizes)");

@@ -50,13 +50,12 @@ struct Geom {
 struct DevEval {
     int n;                  // particles of the evaluation
     int masked;             // kick pair with a fast set (two moment classes)
-    int sort_blocks;        // radix-sort tiles: ceil(n / kSortTileItems)
-    int hist_items;         // digit histogram entries: kSortBins * sort_blocks
     int ncell;              // cells of the tree
     int nlev;               // levels of the tree
     int rows;               // 2 * ncell (expansion rows, both classes)
     int np1;                // n + 1 (prefix sum of the fast flags, with its total)
-    uint32_t overflow;      // bit 0: cells, bit 1: levels, bit 2: walk lists; the step must be redone
+    uint32_t overflow;      // bit 0: cells, bit 1: levels, bit 2: walk lists (the step must be redone); bit 3:
+                            // a bounded wait of the sort ran out
     int level_begin[kMaxLevel + 3];   // first cell of each level; [nlev] = ncell
 };
 
@@ -142,7 +141,7 @@ namespace tg {
 
 // buffer slots of tg_ctx::buf
 enum Slot {
-    B_GEOM = 0, B_PARTIAL, B_KEYS0, B_KEYS1, B_VALS0, B_VALS1, B_HIST, B_SCAN_TMP,
+    B_GEOM = 0, B_KEYS0, B_KEYS1, B_VALS0, B_VALS1, B_SORT, B_SCAN_TMP,
     B_XS, B_YS, B_ZS, B_MS, B_FS, B_PF, B_LEAF_OF,
     B_XS2, B_YS2, B_ZS2, B_MS2, B_FS2, B_PERM2, B_NSLOW,
     B_C_LEVEL, B_C_X, B_C_Y, B_C_Z, B_C_FIRST, B_C_COUNT, B_C_CHILD, B_C_PARENT, B_C_NCHILD,
@@ -184,13 +183,10 @@ struct M2LBlock {
 inline bool m2l_classes_on_device(const tg_ctx *c) { return c->prm.precision == TG_PREC_FP32 && c->prm.p <= 6; }
 
 // ---- tree.cu
-// Root cube of the n particles pos[q] (q < n, gathered through sub when non-null) -> geom.
-tg_status root_cube(tg_ctx *c, int n, const double *pos, int64_t stride, const int64_t *sub, Geom *d_geom,
-                    const int *dn = nullptr);
-// Keys, stable radix sort and gather into sorted order.  Returns device pointers in the ctx
-// slots: B_KEYS0 (sorted keys), B_VALS0 (perm: sorted -> input index q), B_XS.. B_FS.
-tg_status keys_sort_gather(tg_ctx *c, int n, const double *pos, int64_t stride, const int64_t *sub,
-                           const double *mass, const uint8_t *fast, const Geom *d_geom, const DevEval *de = nullptr);
+// Root cube of the n particles pos[q] (q < n, gathered through sub when non-null) -> d_geom, keys, stable radix sort
+// and gather into sorted order: B_KEYS0 (sorted keys), B_VALS0 (perm: sorted -> input index q), B_XS.. B_FS.
+tg_status sort_particles(tg_ctx *c, int n, const double *pos, int64_t stride, const int64_t *sub, const double *mass,
+                         const uint8_t *fast, Geom *d_geom, const DevEval *de = nullptr);
 TreeView tree_view(tg_ctx *c, int n, int ncell);
 
 // ---- octree.cu
@@ -262,24 +258,30 @@ tg_status launch_p2p_f64_dev(tg_ctx *c, const TreeView &t, const DevEval *de, co
                              const uint2 *p2p, size_t cap_p2p, int cap_cells, const double *const xyzm[4],
                              const int32_t *nslow, double *acc4, int stride, int scan_scratch = B_SCAN_TMP);
 
-// Kernels of tree.cu, also launched by the allocation-free sort in noalloc.cu.
+// The sort itself, also used by the allocation-free entry point (noalloc.cu).
 constexpr int kSortTileItems = 2048;     // items per radix-sort block (256 threads x 8)
 constexpr int kSortBits = 9;             // radix digit width: 7 passes cover the 63 key bits
 constexpr int kSortBins = 1 << kSortBits;
 constexpr int kSortPasses = (63 + kSortBits - 1) / kSortBits;
+constexpr int kSmallSort = 8192;         // up to here one block sorts in shared memory
+constexpr int kBoxThreads = 256, kBoxBlocks = 2 * 152;
 constexpr int kScanThreads = 512;        // threads per scan block
-constexpr int kScanTileItems = 2048;     // items per scan block (kScanThreads x 4)
-// (optional device sizes: dn / de, nullptr for host sizes)
-__global__ void scan_tiles(const uint32_t *in, uint32_t *out, uint32_t *tile_sums, int n, const int *dn);
-__global__ void scan_add(uint32_t *out, const uint32_t *tile_pre, int n, const int *dn);
-__global__ void bbox_partial(const double *pos, int64_t stride, const int64_t *sub, int n, double *partial, const int *dn);
-__global__ void bbox_final(const double *partial, int nparts, int n, Geom *g, const int *dn);
-__global__ void morton_keys(const double *pos, int64_t stride, const int64_t *sub, int n, const Geom *g,
-                            uint64_t *keys, uint32_t *vals, const int *dn);
-__global__ void radix_hist(const uint64_t *keys, int n, int shift, uint32_t *hist, int nblocks, const DevEval *de);
-__global__ void radix_scatter(const uint64_t *keys_in, const uint32_t *vals_in, uint64_t *keys_out,
-                              uint32_t *vals_out, const uint32_t *offsets, int n, int shift, int nblocks,
-                              const DevEval *de);
+struct SortScratch {
+    uint32_t *done, *flag;   // blocks of root_cube that finished; 8 when a bounded wait ran out
+    double *boxes;           // a bounding box per block of root_cube
+    uint32_t *state[2];      // digit counts and sums of the tiles, by pass parity
+    uint32_t *hist;          // digit counts of the seven passes, then their tickets
+};
+struct SortedOut {
+    double *x = nullptr, *y = nullptr, *z = nullptr, *m = nullptr;
+    uint8_t *f = nullptr;
+};
+size_t sort_scratch_bytes(int64_t n);
+SortScratch sort_scratch(void *base, int64_t n);
+tg_status ensure_sort_scratch(tg_ctx *c, int64_t n, void **out);
+cudaError_t launch_sort(cudaStream_t st, int n, const int *dn, const double *pos, int64_t stride, const int64_t *sub,
+                        const double *mass, const uint8_t *fast, Geom *g, uint64_t *k0, uint64_t *k1, uint32_t *v0,
+                        uint32_t *v1, const SortScratch &s, const SortedOut &o, bool *swapped, bool *gathered, int *launches);
 
 // ---- fmm.cu
 // Full FMM evaluation on a (sub)set of particles.  Outputs are in input order q:

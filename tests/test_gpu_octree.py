@@ -1,4 +1,5 @@
-"""The octree build (windows of n_crit + 1 keys, cells ranked per level) against the oracle's tree, bit for bit, at
+"""The particle sort at its edges (one block up to 8192 particles, tiles of 2048 above, equal keys in input order)
+and the octree build (windows of n_crit + 1 keys, cells ranked per level) against the oracle's tree, bit for bit, at
 the sizes where it can go wrong: one particle, tiles of 1024 positions and their neighbours, the smallest and
 the largest leaves, few levels, coincident particles (keys equal to the last level) and a far outlier (every
 other particle in one deep corner)."""
@@ -39,3 +40,21 @@ def test_tree_matches_oracle(n, n_crit, kind):
         assert np.array_equal(t["keys"], o.keys) and np.array_equal(t["perm"], o.perm)
         for name in ("level", "coords", "first", "count", "nchild"):
             assert np.array_equal(t[name], getattr(o, name)), name
+
+
+@pytest.mark.parametrize("n", [8191, 8192, 8193, 10240, 10241, 40959, 100001])
+@pytest.mark.parametrize("kind", ["clustered", "coincident", "outlier"])
+def test_sort_matches_oracle(n, kind):
+    pos = _points(kind, n)
+    if kind == "coincident":
+        pos[:, n // 2:] = pos[:, :1]   # one key for almost every particle: the order is the input order
+    s = tg.Solver(tg.Params(p=2, n_crit=64))
+    d = torch.tensor(pos, device=DEV)
+    for _ in range(2):
+        tg.tg_build_tree(s.ctx, d)
+        t = tg.tg_get_tree(s.ctx)
+        k, p = tg.tg_morton_sort_noalloc(d)
+        o = oracle.Tree(pos, oracle.params(n_crit=64))
+        assert np.array_equal(t["keys"], o.keys) and np.array_equal(t["perm"], o.perm)
+        assert np.array_equal(k.cpu().numpy().view(np.uint64), o.keys) and np.array_equal(p.cpu().numpy(), o.perm)
+    s.close()
