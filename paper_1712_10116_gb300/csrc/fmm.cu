@@ -399,7 +399,7 @@ __device__ __forceinline__ double trans_coef<double>(const float *, const double
     return cd[i];
 }
 
-// M2M for the parents of one level, normalised: with d = z_child - z_parent = (+-s/4)^3 and
+// M2M for the parents of one level at orders 7 and 8 (translate.cu up to 6), normalised: with d = z_child - z_parent = (+-s/4)^3 and
 // s_child = s/2,  M~_P^n = sum_children sum_{k <= n} C(n,k) 2^-(2|n-k| + |k|) (+-1)^(n-k) M~_c^k.
 // Block per parent cell.  |n| <= 1 in float64 (M01, threads 0..7), every order also in T (M).
 // Orders >= 2: lane (n, q) with q = lane % 8 sums the terms k <= n (componentwise) of child q,
@@ -410,13 +410,8 @@ constexpr int kM2MThreads = 256;
 
 template <class T>
 __global__ void __launch_bounds__(kM2MThreads) m2m_level(TreeView t, int lb, int le, int p, int nc, int ncp, T *M,
-                                                         double *M01, const DevEval *de, int lvl)
+                                                         double *M01)
 {
-    if (de) {   // level range on the device (batched path); levels past the tree are empty
-        if (lvl + 1 >= de->nlev) return;
-        lb = de->level_begin[lvl];
-        le = de->level_begin[lvl + 1];
-    }
     extern __shared__ __align__(16) unsigned char m2m_smem[];
     T *s_mc = reinterpret_cast<T *>(m2m_smem);   // [8 children][2 classes][ncp]
     const int lane = threadIdx.x & 31, q = lane & 7;
@@ -482,7 +477,7 @@ __global__ void __launch_bounds__(kM2MThreads) m2m_level(TreeView t, int lb, int
     }
 }
 
-// M2L operands: Ms[c][0] = (M~_S + M~_F)/j!, Ms[c][1] = M~_S/j! in precision T (padding zero);
+// M2L operands (full set): Ms[c][0] = (M~_S + M~_F)/j!, Ms[c][1] = M~_S/j! in precision T (padding zero);
 // the monopole and dipole come from the float64 sums.
 // 1/(kx! ky! kz!) for a multi-index past the tables (orders above TG_PMAX)
 __device__ double inv_fact_beyond_tables(int k)
@@ -500,20 +495,23 @@ __device__ double inv_fact_beyond_tables(int k)
 }
 
 template <class T>
-__global__ void scale_moments(int ncell, int nc, int ncp, const T *M, const double *M01, T *Ms, const int *dncell)
+__global__ void scale_moments(int ncell, int masked, int nc, int ncp, const T *M, const double *M01, T *Ms, const DevEval *de)
 {
-    ncell = dev_or(dncell, ncell);
+    if (de) {
+        ncell = de->ncell;
+        masked = de->masked;
+    }
     const int64_t total = (int64_t)ncell * ncp;
     for (int64_t w = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; w < total; w += (int64_t)gridDim.x * blockDim.x) {
         const int64_t c = w / ncp;
         const int k = (int)(w % ncp);
         if (k < 4) {
-            const double mS = M01[(c * 2 + 0) * 4 + k], mF = M01[(c * 2 + 1) * 4 + k];
+            const double mS = M01[(c * 2 + 0) * 4 + k], mF = masked ? M01[(c * 2 + 1) * 4 + k] : 0.0;
             const double f = c_inv_fact[k];
             Ms[(c * 2 + 0) * ncp + k] = (T)((mS + mF) * f);
             Ms[(c * 2 + 1) * ncp + k] = (T)(mS * f);
         } else {
-            const T mS = M[(c * 2 + 0) * ncp + k], mF = M[(c * 2 + 1) * ncp + k];
+            const T mS = M[(c * 2 + 0) * ncp + k], mF = masked ? M[(c * 2 + 1) * ncp + k] : T(0);
             const T f = k < nc ? (k < TG_NCOEF_MAX ? inv_fact_t<T>(k) : (T)inv_fact_beyond_tables(k)) : T(0);
             Ms[(c * 2 + 0) * ncp + k] = (mS + mF) * f;
             Ms[(c * 2 + 1) * ncp + k] = mS * f;
@@ -683,7 +681,7 @@ __global__ void mac_params_dev(const Geom *g, double eps, MacParams *mp)
     if (lf == 0) mp->log2L = log2L;
 }
 
-// ------------------------------------------------------------------ L2L (one level), normalised
+// ------------------------------------------------------------------ L2L (one level, orders 7 and 8), normalised
 // L~_c^n += sum_{d} L~_P^(n+d) (+-1)^d 2^-(2|d| + |n| + 1) / d!  over |d| <= p - |n|.
 // Warp per cell of the level, lanes over the coefficients n >= n_first (1 when only accelerations are
 // wanted: L^0 feeds no force), both classes.  d runs through the
@@ -693,14 +691,8 @@ constexpr int kM2MWarps = 2;   // warps per block of the L2L level kernel
 
 template <class T>
 __global__ void __launch_bounds__(32 * kM2MWarps) l2l_level(TreeView t, int lb, int le, int p, int nc, int ncp, int ncls,
-                                                            int n_first, T *L, const DevEval *de, int lvl)
+                                                            int n_first, T *L)
 {
-    if (de) {   // level range and classes on the device (batched path)
-        if (lvl >= de->nlev) return;
-        lb = de->level_begin[lvl];
-        le = de->level_begin[lvl + 1];
-        ncls = de->masked ? 2 : 1;
-    }
     extern __shared__ __align__(16) unsigned char l2l_smem[];
     T *s_lp = reinterpret_cast<T *>(l2l_smem) + (size_t)(threadIdx.x >> 5) * 2 * ncp;   // parent's L, this warp
     const int lane = threadIdx.x & 31;
@@ -1057,27 +1049,45 @@ static tg_status eval_typed(tg_ctx *c, int n, int ncell, const TreeView &t, cons
                                                                                      ncp, M, M01);
     }
     const int nlev = (int)c->level_begin.size() - 1;
+    const bool fixed = p <= 6, harm = m2l_harmonic(c);
     for (int l = nlev - 2; l >= 0; --l) {
         const int lb = c->level_begin[l], le = c->level_begin[l + 1];
         if (high) {
             if ((st = launch_m2m_hi<T>(c, t, lb, le, p, nc, ncp, M, M01))) return st;
-            continue;
+        } else if (fixed) {
+            launch_m2m_fixed<T>(c, t, lb, le, p, ncp, masked, M, M01, nullptr, 0);
+        } else {
+            ProfScope ps_(c, TG_K_UP);
+            m2m_level<T><<<std::min(le - lb, c->num_sms * 8), kM2MThreads, 8 * 2 * ncp * sizeof(T), c->stream>>>(
+                t, lb, le, p, nc, ncp, M, M01);
         }
-        ProfScope ps_(c, TG_K_UP);
-        m2m_level<T><<<std::min(le - lb, c->num_sms * 8), kM2MThreads, 8 * 2 * ncp * sizeof(T), c->stream>>>(
-            t, lb, le, p, nc, ncp, M, M01, nullptr, 0);
     }
-    {
+    // what M2L reads and adds to: the harmonic set (Mr, Lr) or the full one (Ms, L)
+    const int ncpr = m2l_harmonic_row(p);
+    T *src = Ms, *dst = L;
+    int row = ncp;
+    if (harm) {
+        if ((st = ensure_t(c, B_MOMH, (size_t)ncell * 2 * ncpr, &src)) ||
+            (st = ensure_t(c, B_LOCH, (size_t)ncell * 2 * ncpr, &dst)))
+            return st;
+        row = ncpr;
+        launch_m2l_moments<T>(c, ncell, p, ncp, masked, M, M01, src, ncpr, nullptr);
+    } else {
         ProfScope ps_(c, TG_K_UP);
-        scale_moments<T><<<grid_for((int64_t)ncell * ncp, 256), 256, 0, c->stream>>>(ncell, nc, ncp, M, M01, Ms, nullptr);
+        scale_moments<T><<<grid_for((int64_t)ncell * ncp, 256), 256, 0, c->stream>>>(ncell, masked || !fixed, nc, ncp, M, M01,
+                                                                                    Ms, nullptr);
     }
-    cudaMemsetAsync(L, 0, sizeof(T) * (size_t)ncell * 2 * ncp, c->stream);
+    cudaMemsetAsync(dst, 0, sizeof(T) * (size_t)ncell * 2 * row, c->stream);
     const M2LBlock *blocks = static_cast<const M2LBlock *>(c->buf[B_M2L].p);
     const uint2 *p2p = static_cast<const uint2 *>(c->buf[B_P2P].p);
     uint32_t *fpre = nullptr;
-    if (masked && p <= 6 && (st = fast_prefix(c, fs, n, &fpre, nullptr))) return st;   // the fixed-order M2L kernels
-    if (n_blocks > 0 && (st = launch_m2l_t(c, t, blocks, n_blocks, Ms, L, p, nc, ncp, masked, want_pot, fpre))) return st;
-    for (int l = 1; l < nlev; ++l) {
+    if (masked && fixed && (st = fast_prefix(c, fs, n, &fpre, nullptr))) return st;
+    if (n_blocks > 0 && (st = launch_m2l_t(c, t, blocks, n_blocks, src, dst, p, nc, row, masked, want_pot, fpre))) return st;
+    if (fixed)   // the root goes with level 1
+        for (int l = 1; l <= std::max(1, nlev - 1); ++l)
+            launch_l2l_fixed<T>(c, t, l == 1 ? 0 : c->level_begin[l], c->level_begin[std::min(l, nlev - 1) + 1], p, ncp, ncls,
+                                L, harm ? dst : nullptr, ncpr, nullptr, 0);
+    for (int l = 1; l < nlev && !fixed; ++l) {
         const int lb = c->level_begin[l], le = c->level_begin[l + 1];
         if (high) {
             if ((st = launch_l2l_hi<T>(c, t, lb, le, p, nc, ncp, ncls, want_pot ? 0 : 1, L))) return st;
@@ -1085,8 +1095,7 @@ static tg_status eval_typed(tg_ctx *c, int n, int ncell, const TreeView &t, cons
         }
         ProfScope ps_(c, TG_K_DOWN);
         l2l_level<T><<<grid_for((int64_t)(le - lb) * 32, 32 * kM2MWarps), 32 * kM2MWarps,
-                       kM2MWarps * 2 * ncp * sizeof(T), c->stream>>>(t, lb, le, p, nc, ncp, ncls,
-                                                                     want_pot ? 0 : 1, L, nullptr, 0);
+                       kM2MWarps * 2 * ncp * sizeof(T), c->stream>>>(t, lb, le, p, nc, ncp, ncls, want_pot ? 0 : 1, L);
     }
     if (high) {
         if ((st = launch_l2p_hi<T, T4>(c, n, t, pf, leaf_of, fs, masked, p, ncp, L, acc4))) return st;
@@ -1379,16 +1388,23 @@ static tg_status fmm_eval_dev_t(tg_ctx *c, DevEval *de, const BatchCaps &cap, co
         p2m_leaves<T, T4><<<grid_for((int64_t)cap.cells * 32, 128), 128, 0, c->stream>>>(
             t, d_geom, xs2, ys2, zs2, ms2, fs2, pf, p, nc, ncp, M, M01);
     }
-    for (int l = cap.levels - 1; l >= 0; --l) {
+    for (int l = cap.levels - 1; l >= 0; --l) launch_m2m_fixed<T>(c, t, 0, 0, p, ncp, true, M, M01, de, l);
+    const bool harm = m2l_harmonic(c);
+    const int ncpr = m2l_harmonic_row(p), row = harm ? ncpr : ncp;
+    T *src = Ms, *dst = L;
+    if (harm) {
+        if ((st = ensure_t(c, B_MOMH, rows * ncpr, &src)) || (st = ensure_t(c, B_LOCH, rows * ncpr, &dst))) {
+            cudaStreamWaitEvent(c->stream, c->ev_join, 0);   // no unjoined work on the side stream
+            return st;
+        }
+        launch_m2l_moments<T>(c, cap.cells, p, ncp, true, M, M01, src, ncpr, de);
+    } else {
         ProfScope ps_(c, TG_K_UP);
-        m2m_level<T><<<c->num_sms * 8, kM2MThreads, 8 * 2 * ncp * sizeof(T), c->stream>>>(t, 0, 0, p, nc, ncp, M, M01,
-                                                                                          de, l);
+        scale_moments<T><<<grid_for((int64_t)cap.cells * ncp, 256), 256, 0, c->stream>>>(cap.cells, 1, nc, ncp, M, M01, Ms, de);
     }
     {
         ProfScope ps_(c, TG_K_UP);
-        scale_moments<T><<<grid_for((int64_t)cap.cells * ncp, 256), 256, 0, c->stream>>>(cap.cells, nc, ncp, M, M01, Ms,
-                                                                                        &de->ncell);
-        zero_rows_dev<T><<<c->num_sms * 4, 256, 0, c->stream>>>(L, &de->rows, ncp);
+        zero_rows_dev<T><<<c->num_sms * 4, 256, 0, c->stream>>>(dst, &de->rows, row);
     }
     cudaStreamWaitEvent(c->stream, c->ev_walk, 0);   // M2L reads the walk's blocks
     uint32_t *fpre = nullptr;
@@ -1396,21 +1412,18 @@ static tg_status fmm_eval_dev_t(tg_ctx *c, DevEval *de, const BatchCaps &cap, co
     if (!st) {
         if (sizeof(T) == 4)
             st = launch_m2l_f32_dev(c, t, de, d_geom, blocks, wctr + 1, (int64_t)cap.blocks,
-                                    reinterpret_cast<const float *>(Ms), reinterpret_cast<float *>(L), p, ncp, cap.cells,
+                                    reinterpret_cast<const float *>(src), reinterpret_cast<float *>(dst), p, row, cap.cells,
                                     cap.m2l_src, fpre);
         else
             st = launch_m2l_f64_dev(c, t, de, d_geom, blocks, wctr + 1, (int64_t)cap.blocks,
-                                    reinterpret_cast<const double *>(Ms), reinterpret_cast<double *>(L), p, ncp, fpre);
+                                    reinterpret_cast<const double *>(src), reinterpret_cast<double *>(dst), p, row, fpre);
     }
     if (st) {
         cudaStreamWaitEvent(c->stream, c->ev_join, 0);   // no unjoined work on the side stream
         return st;
     }
-    for (int l = 1; l <= cap.levels; ++l) {
-        ProfScope ps_(c, TG_K_DOWN);
-        l2l_level<T><<<c->num_sms * 16, 32 * kM2MWarps, kM2MWarps * 2 * ncp * sizeof(T), c->stream>>>(
-            t, 0, 0, p, nc, ncp, 2, 1, L, de, l);
-    }
+    for (int l = 1; l <= cap.levels; ++l)
+        launch_l2l_fixed<T>(c, t, 0, 0, p, ncp, 2, L, harm ? dst : nullptr, ncpr, de, l);
     {
         ProfScope ps_(c, TG_K_DOWN);
         const int g = grid_for(cap.n, 128);

@@ -9,14 +9,6 @@
 
 namespace tg {
 
-// zero rows[0] rows of `width` values (device row count)
-template <class T>
-__global__ void zero_rows(T *p, const int *rows, int width)
-{
-    const int64_t n = (int64_t)*rows * width;
-    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) p[i] = T(0);
-}
-
 // zero n (+ extra) words, n from the device when dn is given (dn[0] + extra)
 __global__ void zero_u32(uint32_t *p, int n, const int *dn, int extra)
 {
@@ -85,46 +77,29 @@ static void m2l_directed_launch(tg_ctx *c, const TreeView &t, const uint32_t *of
 #undef TG_DIR
 }
 
-// Harmonic set (G = -1/|d|, P <= 6): fold the moments, contract the reduced sets into Lr, complete L.
+// Harmonic set (G = -1/|d|, P <= 6): Mr and Lr hold the reduced coefficients, Lr starts at zero.
 template <int P>
-static tg_status m2l_f32_harmonic(tg_ctx *c, const TreeView &t, const M2LBlock *blocks, int64_t nblocks, const float *Ms,
-                                  float *L, int ncp, bool masked, bool pot, int grid, const uint32_t *fpre)
+static tg_status m2l_f32_harmonic(tg_ctx *c, const TreeView &t, const M2LBlock *blocks, int64_t nblocks, const float *Mr,
+                                  float *Lr, int ncpr, bool masked, bool pot, int grid, const uint32_t *fpre)
 {
+    tg_status st;
     if (c->tune.m2l_form == 1) {
         // directed by target cell
-        constexpr int NH = M2LGenH<P>::NC;
-        const int ncpr = (NH + 3) & ~3;
         const int ncell = t.ncell;
-        const int64_t rows = (int64_t)ncell * 2;
         const uint64_t cap = 2ull * (uint64_t)c->last_nm2l + 16;
-        float *Mr, *Lr;
         uint32_t *cnt, *off, *fill, *src;
-        tg_status st;
-        if ((st = ensure_t(c, B_MOMH, (size_t)rows * ncpr, &Mr)) || (st = ensure_t(c, B_LOCH, (size_t)rows * ncpr, &Lr)) ||
-            (st = ensure_t(c, B_M2L_CNT, (size_t)ncell, &cnt)) || (st = ensure_t(c, B_M2L_OFF, (size_t)ncell, &off)) ||
+        if ((st = ensure_t(c, B_M2L_CNT, (size_t)ncell, &cnt)) || (st = ensure_t(c, B_M2L_OFF, (size_t)ncell, &off)) ||
             (st = ensure_t(c, B_M2L_FILL, (size_t)ncell, &fill)) || (st = ensure_t(c, B_M2L_SRC, cap, &src)))
             return st;
         if ((st = m2l_lists(c, t, blocks, nblocks, ncell, cnt, off, fill, src, cap, nullptr, nullptr))) return st;
         ProfScope ps_(c, TG_K_M2L);
-        m2l_reduce_moments_h<P, float><<<grid_for(rows, 128), 128, 0, c->stream>>>(rows, Ms, ncp, Mr, ncpr, nullptr);
-        cudaMemsetAsync(Lr, 0, sizeof(float) * (size_t)rows * ncpr, c->stream);
         m2l_directed_launch<P>(c, t, off, cnt, src, cap, Mr, Lr, ncpr, masked, pot, nullptr);
-        m2l_complete_locals_h<P, float><<<grid_for(rows, 128), 128, 0, c->stream>>>(rows, Lr, ncpr, L, ncp, nullptr);
         return cuda_check(c, cudaGetLastError(), "m2l launch (directed)");
     }
-    constexpr int NH = M2LGenH<P>::NC;
-    const int ncpr = (NH + 3) & ~3;
-    const int64_t rows = (int64_t)t.ncell * 2;
-    float *Mr, *Lr;
     M2LBlock *part;
     unsigned long long *pcnt;
-    tg_status st;
-    if ((st = ensure_t(c, B_MOMH, (size_t)rows * ncpr, &Mr)) || (st = ensure_t(c, B_LOCH, (size_t)rows * ncpr, &Lr)))
-        return st;
     if ((st = m2l_partition_blocks(c, blocks, nblocks, nullptr, &part, &pcnt))) return st;
     ProfScope ps_(c, TG_K_M2L);
-    m2l_reduce_moments_h<P, float><<<grid_for(rows, 128), 128, 0, c->stream>>>(rows, Ms, ncp, Mr, ncpr, nullptr);
-    cudaMemsetAsync(Lr, 0, sizeof(float) * (size_t)rows * ncpr, c->stream);
     using G = M2LHarm<P>;
 #define TG_M2L_H(MK, PT)                                                                                          \
     do {                                                                                                          \
@@ -139,7 +114,6 @@ static tg_status m2l_f32_harmonic(tg_ctx *c, const TreeView &t, const M2LBlock *
         else TG_M2L_H(false, false);
     }
 #undef TG_M2L_H
-    m2l_complete_locals_h<P, float><<<grid_for(rows, 128), 128, 0, c->stream>>>(rows, Lr, ncpr, L, ncp, nullptr);
     return cuda_check(c, cudaGetLastError(), "m2l launch");
 }
 
@@ -150,8 +124,7 @@ tg_status launch_m2l_f32(tg_ctx *c, const TreeView &t, const M2LBlock *blocks, i
     const float eoL = (float)ldexp(c->prm.eps, -c->walk_log2L);
     if (p > TG_PMAX) return launch_m2l_hi<float>(c, t, blocks, nblocks, Ms, L, p, nc, ncp, masked, pot);
     const int grid = grid_for(nblocks * 32, 128, c->num_sms * c->tune.m2l_blocks_per_sm);
-    // Wendland C2: the walk's eps gap rule leaves every M2L pair at r >= eps, where G = -1/r is harmonic
-    if (!plummer && p >= 1 && p <= 6) {
+    if (m2l_harmonic(c)) {
         switch (p) {
         case 1: return m2l_f32_harmonic<1>(c, t, blocks, nblocks, Ms, L, ncp, masked, pot, grid, fpre);
         case 2: return m2l_f32_harmonic<2>(c, t, blocks, nblocks, Ms, L, ncp, masked, pot, grid, fpre);
@@ -208,15 +181,12 @@ __global__ void m2l_list_check(const uint32_t *off, const uint32_t *cnt, DevEval
 template <int P>
 static tg_status m2l_f32_dev_p(tg_ctx *c, const TreeView &t, const DevEval *de, const Geom *gp, const M2LBlock *blocks,
                                const unsigned long long *dnb, int64_t cap_blocks, const float *Ms, float *L, int ncp,
-                               float *Mr, float *Lr, int ncpr, int rows_cap, int grid, size_t cap_src,
-                               const uint32_t *fpre)
+                               int cap_cells, int grid, size_t cap_src, const uint32_t *fpre)
 {
-    const int plummer = c->prm.kernel == TG_KERNEL_PLUMMER;
-    const int g = grid_for(rows_cap, 128);
-    if (!plummer && c->tune.m2l_form == 1) {
-        const int cap_cells = rows_cap / 2;
+    const bool harm = m2l_harmonic(c);
+    tg_status st;
+    if (harm && c->tune.m2l_form == 1) {
         uint32_t *cnt, *off, *fill, *src;
-        tg_status st;
         if ((st = ensure_t(c, B_M2L_CNT, (size_t)cap_cells, &cnt)) ||
             (st = ensure_t(c, B_M2L_OFF, (size_t)cap_cells, &off)) ||
             (st = ensure_t(c, B_M2L_FILL, (size_t)cap_cells, &fill)) || (st = ensure_t(c, B_M2L_SRC, cap_src, &src)))
@@ -225,34 +195,25 @@ static tg_status m2l_f32_dev_p(tg_ctx *c, const TreeView &t, const DevEval *de, 
             return st;
         ProfScope ps_(c, TG_K_M2L);
         m2l_list_check<<<1, 1, 0, c->stream>>>(off, cnt, const_cast<DevEval *>(de), cap_src);
-        m2l_reduce_moments_h<P, float><<<g, 128, 0, c->stream>>>(rows_cap, Ms, ncp, Mr, ncpr, &de->rows);
-        zero_rows<float><<<c->num_sms * 4, 256, 0, c->stream>>>(Lr, &de->rows, ncpr);
-        m2l_directed_launch<P>(c, t, off, cnt, src, cap_src, Mr, Lr, ncpr, true, false, de);
-        m2l_complete_locals_h<P, float><<<g, 128, 0, c->stream>>>(rows_cap, Lr, ncpr, L, ncp, &de->rows);
+        m2l_directed_launch<P>(c, t, off, cnt, src, cap_src, Ms, L, ncp, true, false, de);
         return TG_OK;
     }
     M2LBlock *part;
     unsigned long long *pcnt;
-    tg_status st;
     if ((st = m2l_partition_blocks(c, blocks, cap_blocks, dnb, &part, &pcnt))) return st;
     ProfScope ps_(c, TG_K_M2L);
-    if (!plummer) {
-        // harmonic set: fold, contract (the launch for the other class count returns at once), complete
-        using G = M2LHarm<P>;
-        m2l_reduce_moments_h<P, float><<<g, 128, 0, c->stream>>>(rows_cap, Ms, ncp, Mr, ncpr, &de->rows);
-        zero_rows<float><<<c->num_sms * 4, 256, 0, c->stream>>>(Lr, &de->rows, ncpr);
-        m2l_blocks_f32<G, true, false><<<grid, 128, 0, c->stream>>>(t, part, cap_blocks, pcnt, Mr, Lr, ncpr, 0.f, 0, de,
-                                                                    gp, c->prm.eps, fpre, c->d_counters + 11);
-        m2l_blocks_f32<G, false, false><<<grid, 128, 0, c->stream>>>(t, part, cap_blocks, pcnt, Mr, Lr, ncpr, 0.f, 0, de,
-                                                                     gp, c->prm.eps, fpre, c->d_counters + 11);
-        m2l_complete_locals_h<P, float><<<g, 128, 0, c->stream>>>(rows_cap, Lr, ncpr, L, ncp, &de->rows);
+    // the launch for the other class count returns at once
+#define TG_M2L_DEV(G, MK) \
+    m2l_blocks_f32<G, MK, false><<<grid, 128, 0, c->stream>>>(t, part, cap_blocks, pcnt, Ms, L, ncp, 0.f, !harm, de, gp, \
+                                                              c->prm.eps, fpre, c->d_counters + 11)
+    if (harm) {
+        TG_M2L_DEV(M2LHarm<P>, true);
+        TG_M2L_DEV(M2LHarm<P>, false);
     } else {
-        using G = M2LFull<P>;
-        m2l_blocks_f32<G, true, false><<<grid, 128, 0, c->stream>>>(t, part, cap_blocks, pcnt, Ms, L, ncp, 0.f, 1, de,
-                                                                    gp, c->prm.eps, fpre, c->d_counters + 11);
-        m2l_blocks_f32<G, false, false><<<grid, 128, 0, c->stream>>>(t, part, cap_blocks, pcnt, Ms, L, ncp, 0.f, 1, de,
-                                                                     gp, c->prm.eps, fpre, c->d_counters + 11);
+        TG_M2L_DEV(M2LFull<P>, true);
+        TG_M2L_DEV(M2LFull<P>, false);
     }
+#undef TG_M2L_DEV
     return TG_OK;
 }
 
@@ -260,59 +221,35 @@ tg_status launch_m2l_f32_dev(tg_ctx *c, const TreeView &t, const DevEval *de, co
                              const unsigned long long *dnb, int64_t cap_blocks, const float *Ms, float *L, int p,
                              int ncp, int cap_cells, size_t cap_src, const uint32_t *fpre)
 {
-    if (p < 1 || p > 6) return set_err(c, TG_ERR_ARG, "batched M2L needs 1 <= p <= 6");
-    static const int nh[7] = {0, 4, 9, 16, 25, 36, 49};   // (p + 1)^2 harmonic coefficients
-    const int ncpr = (nh[p] + 3) & ~3;
-    const int rows_cap = 2 * cap_cells;
-    float *Mr = nullptr, *Lr = nullptr;
-    tg_status st;
-    if (c->prm.kernel != TG_KERNEL_PLUMMER &&
-        ((st = ensure_t(c, B_MOMH, (size_t)rows_cap * ncpr, &Mr)) || (st = ensure_t(c, B_LOCH, (size_t)rows_cap * ncpr, &Lr))))
-        return st;
     const int grid = c->num_sms * c->tune.m2l_blocks_per_sm;
+    tg_status st;
     switch (p) {
-    case 1: st = m2l_f32_dev_p<1>(c, t, de, gp, blocks, dnb, cap_blocks, Ms, L, ncp, Mr, Lr, ncpr, rows_cap, grid, cap_src, fpre); break;
-    case 2: st = m2l_f32_dev_p<2>(c, t, de, gp, blocks, dnb, cap_blocks, Ms, L, ncp, Mr, Lr, ncpr, rows_cap, grid, cap_src, fpre); break;
-    case 3: st = m2l_f32_dev_p<3>(c, t, de, gp, blocks, dnb, cap_blocks, Ms, L, ncp, Mr, Lr, ncpr, rows_cap, grid, cap_src, fpre); break;
-    case 4: st = m2l_f32_dev_p<4>(c, t, de, gp, blocks, dnb, cap_blocks, Ms, L, ncp, Mr, Lr, ncpr, rows_cap, grid, cap_src, fpre); break;
-    case 5: st = m2l_f32_dev_p<5>(c, t, de, gp, blocks, dnb, cap_blocks, Ms, L, ncp, Mr, Lr, ncpr, rows_cap, grid, cap_src, fpre); break;
-    default: st = m2l_f32_dev_p<6>(c, t, de, gp, blocks, dnb, cap_blocks, Ms, L, ncp, Mr, Lr, ncpr, rows_cap, grid, cap_src, fpre);
+    case 4: st = m2l_f32_dev_p<4>(c, t, de, gp, blocks, dnb, cap_blocks, Ms, L, ncp, cap_cells, grid, cap_src, fpre); break;
+    case 5: st = m2l_f32_dev_p<5>(c, t, de, gp, blocks, dnb, cap_blocks, Ms, L, ncp, cap_cells, grid, cap_src, fpre); break;
+    case 6: st = m2l_f32_dev_p<6>(c, t, de, gp, blocks, dnb, cap_blocks, Ms, L, ncp, cap_cells, grid, cap_src, fpre); break;
+    default: return set_err(c, TG_ERR_ARG, "batched M2L needs 4 <= p <= 6");
     }
     if (st) return st;
     return cuda_check(c, cudaGetLastError(), "m2l launch (device sizes)");
 }
 
-// float64, P <= 6: the harmonic set (Wendland) folds the moments, contracts into Lr and completes L; with de every
-// count is on the device (nb and rows are then capacities, and the launch for the other class count returns).
+// float64, P <= 6, over the harmonic or the full set as launch_m2l_f32; with de every count is on the device (nb is
+// then a capacity, and the launch for the other class count returns).
 template <int P>
 static tg_status m2l_f64_p(tg_ctx *c, const TreeView &t, const M2LBlock *blocks, int64_t nb, const double *Ms, double *L,
                            int ncp, bool masked, bool pot, const uint32_t *fpre, const DevEval *de, const Geom *gp,
                            const unsigned long long *dnb)
 {
-    const bool plummer = c->prm.kernel == TG_KERNEL_PLUMMER;
+    const bool harm = m2l_harmonic(c);
     const double eoL = de ? 0.0 : ldexp(c->prm.eps, -c->walk_log2L);
     const int grid = c->num_sms * 4;
-    constexpr int NH = M2LGenH<P>::NC;
-    const int ncpr = (NH + 3) & ~3;
-    const int64_t rows = (int64_t)t.ncell * 2;
-    const int *drows = de ? &de->rows : nullptr;
-    double *Mr = nullptr, *Lr = nullptr;
-    tg_status st;
-    if (!plummer && ((st = ensure_t(c, B_MOMH, (size_t)rows * ncpr, &Mr)) || (st = ensure_t(c, B_LOCH, (size_t)rows * ncpr, &Lr))))
-        return st;
     ProfScope ps_(c, TG_K_M2L);
-    if (!plummer) {
-        m2l_reduce_moments_h<P, double><<<grid_for(rows, 128), 128, 0, c->stream>>>(rows, Ms, ncp, Mr, ncpr, drows);
-        if (de) zero_rows<double><<<c->num_sms * 4, 256, 0, c->stream>>>(Lr, drows, ncpr);
-        else cudaMemsetAsync(Lr, 0, sizeof(double) * (size_t)rows * ncpr, c->stream);
-    }
-#define TG_M2L64_(G, MK, PT, MS, LL, NCP)                                                                          \
-    m2l_pairs_f64<G, MK, PT><<<grid, 128, 0, c->stream>>>(t, blocks, nb, dnb, MS, LL, NCP, eoL, plummer, de, gp,    \
-                                                          c->prm.eps, fpre)
+#define TG_M2L64_(G, MK, PT)                                                                                       \
+    m2l_pairs_f64<G, MK, PT><<<grid, 128, 0, c->stream>>>(t, blocks, nb, dnb, Ms, L, ncp, eoL, !harm, de, gp, c->prm.eps, fpre)
 #define TG_M2L64(MK, PT)                                                                                           \
     do {                                                                                                           \
-        if (plummer) TG_M2L64_(M2LFull<P>, MK, PT, Ms, L, ncp);                                                    \
-        else TG_M2L64_(M2LHarm<P>, MK, PT, Mr, Lr, ncpr);                                                          \
+        if (harm) TG_M2L64_(M2LHarm<P>, MK, PT);                                                                   \
+        else TG_M2L64_(M2LFull<P>, MK, PT);                                                                        \
     } while (0)
     if (de) {
         TG_M2L64(true, false);
@@ -326,8 +263,6 @@ static tg_status m2l_f64_p(tg_ctx *c, const TreeView &t, const M2LBlock *blocks,
     }
 #undef TG_M2L64
 #undef TG_M2L64_
-    if (!plummer)
-        m2l_complete_locals_h<P, double><<<grid_for(rows, 128), 128, 0, c->stream>>>(rows, Lr, ncpr, L, ncp, drows);
     return cuda_check(c, cudaGetLastError(), "m2l launch (float64)");
 }
 

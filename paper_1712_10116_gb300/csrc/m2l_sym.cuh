@@ -75,31 +75,6 @@ __host__ __device__ constexpr int order_in(bool harmonic, int k)
     return o;
 }
 
-// per cell and class: fold the moments onto j_z <= 1 (pads zeroed)
-template <int P, class T>
-__global__ void m2l_reduce_moments_h(int64_t nrows, const T *__restrict__ Ms, int ncp, T *__restrict__ Mr, int ncpr,
-                                     const int *drows)
-{
-    if (drows) nrows = *drows;
-    for (int64_t w = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; w < nrows; w += (int64_t)gridDim.x * blockDim.x) {
-        M2LGenH<P>::reduce_moments(Ms + w * ncp, Mr + w * ncpr);
-        for (int k = M2LGenH<P>::NC; k < ncpr; ++k) Mr[w * ncpr + k] = T(0);
-    }
-}
-
-// per cell and class: the full local expansion from its n_z <= 1 coefficients (pads zeroed)
-template <int P, class T>
-__global__ void m2l_complete_locals_h(int64_t nrows, const T *__restrict__ Lr, int ncpr, T *__restrict__ L, int ncp,
-                                      const int *drows)
-{
-    if (drows) nrows = *drows;
-    constexpr int NC = M2LGen<P>::NC;
-    for (int64_t w = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; w < nrows; w += (int64_t)gridDim.x * blockDim.x) {
-        M2LGenH<P>::complete_locals(Lr + w * ncpr, L + w * ncp);
-        for (int k = NC; k < ncp; ++k) L[w * ncp + k] = T(0);
-    }
-}
-
 // halve the live coefficients once: lanes with bit d keep the upper half, the others the lower half
 template <int NP, int H>
 __device__ __forceinline__ void m2l_halve(float (&v)[NP], int lane, int d)

@@ -229,6 +229,22 @@ tg_status injected_alloc_failure(tg_ctx *c, size_t bytes, int slot);
 tg_status exclusive_scan_u32(tg_ctx *c, const uint32_t *in, uint32_t *out, int n, uint32_t *d_total,
                              const int *dn = nullptr, int scratch = B_SCAN_TMP);
 
+// ---- translate.cu: M2M and L2L of one level at orders up to 6, and the moments the harmonic M2L reads.  With de the
+// level range and the classes come from the device.  Lr: harmonic M2L sums (null: L holds the full set's).
+template <class T>
+void launch_m2m_fixed(tg_ctx *c, const TreeView &t, int lb, int le, int p, int ncp, bool masked, T *M, double *M01,
+                      const DevEval *de, int lvl);
+template <class T>
+void launch_l2l_fixed(tg_ctx *c, const TreeView &t, int lb, int le, int p, int ncp, int ncls, T *L, const T *Lr, int ncpr,
+                      const DevEval *de, int lvl);
+template <class T>
+void launch_m2l_moments(tg_ctx *c, int ncell, int p, int ncp, bool masked, const T *M, const double *M01, T *Mr, int ncpr,
+                        const DevEval *de);
+// Wendland C2: the walk's eps gap rule leaves every M2L pair at r >= eps, where G = -1/r is harmonic: M2L then reads and
+// sums the (p + 1)^2 coefficients with k_z <= 1 (rows of m2l_harmonic_row(p)).
+inline bool m2l_harmonic(const tg_ctx *c) { return c->prm.kernel != TG_KERNEL_PLUMMER && c->prm.p <= 6; }
+inline int m2l_harmonic_row(int p) { return ((p + 1) * (p + 1) + 3) & ~3; }
+
 // ---- m2l.cu: mutual M2L of the walk's blocks into L (normalised expansions).  pot = false: the
 // float32 kernels leave out the potential term L^0.  fpre (kick pairs, nullable): prefix sum of the fast
 // flags of the sorted particles, so that contractions no target needs are skipped.
