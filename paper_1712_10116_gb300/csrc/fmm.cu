@@ -558,6 +558,12 @@ __device__ __forceinline__ unsigned long long warp_reserve(unsigned long long *c
 
 // One step of the dual walk.  The input length is read on the device (it is the previous step's
 // output counter), so that all steps can be queued without waiting for the host.
+// A thread classifies all (up to 64) child pairs of a frontier pair, which serves long frontiers best: with eight
+// lanes per pair (one per row) the leaf rows of half-opened pairs leave lanes idle, 2.05 -> 3.05 ms for the walk of
+// the disk galaxy.  A frontier so short that the grid has eight threads for each of its pairs is bound by that
+// serial chain instead, and then eight lanes share a pair: the walk of 1021 particles took 127 us and takes 70,
+// of 54,321 190 and 155, of the disk galaxy (its first and last steps) 1.34 ms and 1.25.  Switching at 2, 4, 8 or 16
+// threads per pair made no further difference.
 __device__ __forceinline__ void walk_step_body(const TreeView &t, const MacParams &mp, const uint2 *front_in,
                                                const unsigned long long *n_in_ctr, const WalkOut &o)
 {
@@ -565,23 +571,26 @@ __device__ __forceinline__ void walk_step_body(const TreeView &t, const MacParam
     const int64_t n_in = (int64_t)(n_in_raw < o.cap_front ? n_in_raw : o.cap_front);
     // whole warps iterate together so that the counters can be reserved per warp
     const int64_t stride = (int64_t)gridDim.x * blockDim.x;
-    for (int64_t w0 = (int64_t)blockIdx.x * blockDim.x; w0 < n_in; w0 += stride) {
+    const bool wide = 8 * n_in <= stride;
+    const int64_t n_items = wide ? 8 * n_in : n_in;
+    for (int64_t w0 = (int64_t)blockIdx.x * blockDim.x; w0 < n_items; w0 += stride) {
         const int64_t w = w0 + threadIdx.x;
-        const bool active = w < n_in;
+        const bool active = w < n_items;
         int A = 0, B = 0, ni = 0, nj = 0, baseA = 0, baseB = 0;
         bool self = false;
-        // classes of the child pairs, bit 8i + j: well separated (M2L), P2P, self P2P, frontier
+        // classes of the child pairs, bit 8i + j: well separated (M2L), P2P, self P2P, frontier (wide: of row i only)
         unsigned long long mask = 0, mp2p = 0, mself = 0, mfront = 0;
         if (active) {
-            const uint2 pr = front_in[w];
+            const uint2 pr = front_in[wide ? w >> 3 : w];
             A = (int)pr.x;
             B = (int)pr.y;
             self = A == B;
-            const bool openA = t.nchild[A] != 0, openB = t.nchild[B] != 0;
-            ni = openA ? t.nchild[A] : 1;
-            nj = openB ? t.nchild[B] : 1;
-            baseA = openA ? t.child_first[A] : A;
-            baseB = openB ? t.child_first[B] : B;
+            const int ncA = t.nchild[A], ncB = t.nchild[B], cfA = t.child_first[A], cfB = t.child_first[B];
+            ni = ncA ? ncA : 1;
+            nj = ncB ? ncB : 1;
+            baseA = ncA ? cfA : A;
+            baseB = ncB ? cfB : B;
+            const int i_begin = wide ? (int)(w & 7) : 0, i_end = wide ? min(i_begin + 1, ni) : ni;
             // the column cells' geometry, loaded once (independent loads, issued together)
             CellGeo gy[8];
             bool ly[8];
@@ -592,7 +601,7 @@ __device__ __forceinline__ void walk_step_body(const TreeView &t, const MacParam
                 ly[j] = t.nchild[y] == 0;
             }
             // classify every child pair once
-            for (int i = 0; i < ni; ++i) {
+            for (int i = i_begin; i < i_end; ++i) {
                 const int x = baseA + i;
                 const CellGeo gx{t.cx[x], t.cy[x], t.cz[x], (int)t.level[x]};
                 const bool lx = t.nchild[x] == 0;
@@ -617,8 +626,13 @@ __device__ __forceinline__ void walk_step_body(const TreeView &t, const MacParam
         unsigned long long fb = warp_reserve(o.front_ctr, (unsigned)__popcll(mfront));
         unsigned long long pb = warp_reserve(o.counters + 2, (unsigned)__popcll(mp2p));
         unsigned long long sb = warp_reserve(o.counters + 4, (unsigned)__popcll(mself));
-        const unsigned long long bb = warp_reserve(o.counters + 1, mask ? 1u : 0u);
         warp_reserve(o.counters + 3, (unsigned)__popcll(mask));
+        if (wide) {   // the block of the pair's eight rows, written by its first lane
+#pragma unroll
+            for (int d = 1; d < 8; d <<= 1) mask |= __shfl_xor_sync(0xffffffffu, mask, d);
+            if (w & 7) mask = 0ull;
+        }
+        const unsigned long long bb = warp_reserve(o.counters + 1, mask ? 1u : 0u);
         if (!active) continue;
         if (mask && bb < o.cap_blocks) o.blocks[bb] = M2LBlock{(uint32_t)A, (uint32_t)B, mask};
         // write the entries of each class from its bits (lowest bit first, the order of the loops above)
