@@ -323,8 +323,13 @@ __device__ __forceinline__ int warp_incl_scan(int v, int lane)
 // of A with a larger index, i.e. each slow-slow and slow-fast pair once (p2p_pair_f32, SELF).
 // Batched path (walk_ctr non-null): the root cube comes from gp and the self pairs from the walk's
 // counters on the device (they sit at the end of the P2P buffer of capacity cap_p2p).
+//
+// Bound by the latency of dependent packed operations: three blocks of 256 per SM (80 registers a thread, part of the
+// units' bookkeeping spilled) beat two (128 registers) although they spill.  Two rows per lane: disk galaxy 15.9
+// against 17.1 ms, 2^20 sphere 5.45 against 5.67; one row 18.3 against 19.7 and 6.50 against 6.77.  Three rows keep
+// two blocks (17.1 and 5.38; three blocks: 18.4 and 5.46).
 template <int KERNEL, int ROWS, bool POT>
-__global__ void __launch_bounds__(256, 2) p2p_owner_f32(TreeView t, int log2L, const uint2 *__restrict__ units,
+__global__ void __launch_bounds__(256, ROWS == 3 ? 2 : 3) p2p_owner_f32(TreeView t, int log2L, const uint2 *__restrict__ units,
                                                         uint32_t *ctr, const uint32_t *__restrict__ own_off,
                                                         const uint32_t *__restrict__ own_cnt,
                                                         const int32_t *__restrict__ partners, int64_t npairs,
