@@ -231,10 +231,14 @@ __global__ void leaf_particles(TreeView t, const Geom *gp, const double *xs, con
 // With classes, every leaf's particles are stably reordered so the slow ones come first
 // (nslow[leaf] of them).  Leaf ranges and the tree are unchanged; a mutual P2P tile can then skip
 // the fast-fast block (kickS2F feels slow masses only) instead of masking it pair by pair.
-__global__ void leaf_class_partition(TreeView t, const double *xs, const double *ys, const double *zs, const double *ms,
+// The same pass writes the particles' local data (leaf_particles serves evaluations without classes).
+template <class T4>
+__global__ void leaf_class_partition(TreeView t, const Geom *gp, const double *xs, const double *ys, const double *zs, const double *ms,
                                      const uint8_t *fs, const uint32_t *perm, double *xs2, double *ys2, double *zs2,
-                                     double *ms2, uint8_t *fs2, uint32_t *perm2, int32_t *nslow)
+                                     double *ms2, uint8_t *fs2, uint32_t *perm2, int32_t *nslow,
+                                     T4 *pf, int32_t *leaf_of)
 {
+    const Geom g = *gp;
     const int warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;
     const int nwarps = (gridDim.x * blockDim.x) >> 5;
     const unsigned lt = (1u << lane) - 1u;
@@ -245,6 +249,7 @@ __global__ void leaf_class_partition(TreeView t, const double *xs, const double 
         int ns = 0;
         for (int q0 = 0; q0 < count; q0 += 32) ns += __popc(__ballot_sync(0xffffffffu, q0 + lane < count && !fs[first + q0 + lane]));
         int slow_seen = 0, fast_seen = 0;
+        const double zx = cell_centre(g, t, c, 0), zy = cell_centre(g, t, c, 1), zz = cell_centre(g, t, c, 2);
         for (int q0 = 0; q0 < count; q0 += 32) {
             const int q = q0 + lane;
             const bool valid = q < count;
@@ -253,10 +258,18 @@ __global__ void leaf_class_partition(TreeView t, const double *xs, const double 
             if (valid) {
                 const int dst = first + (slow ? slow_seen + __popc(bs & lt) : ns + fast_seen + __popc(bf & lt));
                 const int src = first + q;
-                xs2[dst] = xs[src];
-                ys2[dst] = ys[src];
-                zs2[dst] = zs[src];
-                ms2[dst] = ms[src];
+                const double x = xs[src], y = ys[src], z = zs[src], m = ms[src];
+                xs2[dst] = x;
+                ys2[dst] = y;
+                zs2[dst] = z;
+                ms2[dst] = m;
+                T4 v;
+                v.x = (decltype(v.x))(x - zx);
+                v.y = (decltype(v.x))(y - zy);
+                v.z = (decltype(v.x))(z - zz);
+                v.w = (decltype(v.x))m;
+                pf[dst] = v;
+                leaf_of[dst] = c;
                 fs2[dst] = fs[src];
                 perm2[dst] = perm[src];
             }
@@ -879,18 +892,6 @@ __global__ void scatter_out(int n, const uint32_t *perm, const double *acc4, dou
     }
 }
 
-// zero the three acceleration rows of an acc4 array for the first dn[0] particles
-__global__ void zero_acc3(double *acc4, int64_t stride4, const int *dn)
-{
-    const int n = dn[0];
-    for (int s = blockIdx.x * blockDim.x + threadIdx.x; s < n; s += gridDim.x * blockDim.x) {
-        acc4[s] = 0.0;
-        acc4[(size_t)stride4 + s] = 0.0;
-        acc4[2 * (size_t)stride4 + s] = 0.0;
-    }
-}
-
-
 // ------------------------------------------------------------------ orchestration
 __global__ void walk_init(uint2 *front, unsigned long long *front_ctr)
 {
@@ -981,14 +982,14 @@ static inline int pad4(int x) { return (x + 3) & ~3; }
 
 // precision dispatch of the M2L and P2P launchers (m2l.cu, p2p.cu)
 static tg_status launch_m2l_t(tg_ctx *c, const TreeView &t, const M2LBlock *blocks, int64_t nblocks, const float *Ms,
-                              float *L, int p, int nc, int ncp, bool masked, bool pot, const uint32_t *fpre)
+                              float *L, int p, int nc, int ncp, bool masked, bool pot, const int32_t *nslow)
 {
-    return launch_m2l_f32(c, t, blocks, nblocks, Ms, L, p, nc, ncp, masked, pot, fpre);
+    return launch_m2l_f32(c, t, blocks, nblocks, Ms, L, p, nc, ncp, masked, pot, nslow);
 }
 static tg_status launch_m2l_t(tg_ctx *c, const TreeView &t, const M2LBlock *blocks, int64_t nblocks, const double *Ms,
-                              double *L, int p, int nc, int ncp, bool masked, bool pot, const uint32_t *fpre)
+                              double *L, int p, int nc, int ncp, bool masked, bool pot, const int32_t *nslow)
 {
-    return launch_m2l_f64(c, t, blocks, nblocks, Ms, L, p, nc, ncp, masked, pot, fpre);
+    return launch_m2l_f64(c, t, blocks, nblocks, Ms, L, p, nc, ncp, masked, pot, nslow);
 }
 static tg_status launch_p2p_t(tg_ctx *c, const TreeView &t, const uint2 *pairs, int64_t npairs, const uint2 *self_pairs,
                               int64_t nself, const float4 *pf, const double *const xyzm[4], const int32_t *nslow,
@@ -1035,8 +1036,9 @@ static tg_status eval_typed(tg_ctx *c, int n, int ncell, const TreeView &t, cons
             return st;
         {
             ProfScope ps_(c, TG_K_TREE);
-            leaf_class_partition<<<grid_for((int64_t)ncell * 32, 256), 256, 0, c->stream>>>(
-                t, xs, ys, zs, ms, fs, static_cast<const uint32_t *>(c->buf[B_VALS0].p), xs2, ys2, zs2, ms2, fs2, perm2, nslow);
+            leaf_class_partition<T4><<<grid_for((int64_t)ncell * 32, 256), 256, 0, c->stream>>>(
+                t, d_geom, xs, ys, zs, ms, fs, static_cast<const uint32_t *>(c->buf[B_VALS0].p), xs2, ys2, zs2, ms2, fs2, perm2,
+                nslow, pf, leaf_of);
         }
         std::swap(c->buf[B_XS], c->buf[B_XS2]);
         std::swap(c->buf[B_YS], c->buf[B_YS2]);
@@ -1049,8 +1051,7 @@ static tg_status eval_typed(tg_ctx *c, int n, int ncell, const TreeView &t, cons
         zs = zs2;
         ms = ms2;
         fs = fs2;
-    }
-    {
+    } else {
         ProfScope ps_(c, TG_K_UP);
         leaf_particles<T4><<<grid_for((int64_t)ncell * 32, 256), 256, 0, c->stream>>>(t, d_geom, xs, ys, zs, ms, pf, leaf_of);
     }
@@ -1069,7 +1070,7 @@ static tg_status eval_typed(tg_ctx *c, int n, int ncell, const TreeView &t, cons
         if (high) {
             if ((st = launch_m2m_hi<T>(c, t, lb, le, p, nc, ncp, M, M01))) return st;
         } else if (fixed) {
-            launch_m2m_fixed<T>(c, t, lb, le, p, ncp, masked, M, M01, nullptr, 0);
+            launch_m2m_fixed<T>(c, t, lb, le, p, ncp, masked, M, M01, nslow, nullptr, 0);
         } else {
             ProfScope ps_(c, TG_K_UP);
             m2m_level<T><<<std::min(le - lb, c->num_sms * 8), kM2MThreads, 8 * 2 * ncp * sizeof(T), c->stream>>>(
@@ -1094,9 +1095,7 @@ static tg_status eval_typed(tg_ctx *c, int n, int ncell, const TreeView &t, cons
     cudaMemsetAsync(dst, 0, sizeof(T) * (size_t)ncell * 2 * row, c->stream);
     const M2LBlock *blocks = static_cast<const M2LBlock *>(c->buf[B_M2L].p);
     const uint2 *p2p = static_cast<const uint2 *>(c->buf[B_P2P].p);
-    uint32_t *fpre = nullptr;
-    if (masked && fixed && (st = fast_prefix(c, fs, n, &fpre, nullptr))) return st;
-    if (n_blocks > 0 && (st = launch_m2l_t(c, t, blocks, n_blocks, src, dst, p, nc, row, masked, want_pot, fpre))) return st;
+    if (n_blocks > 0 && (st = launch_m2l_t(c, t, blocks, n_blocks, src, dst, p, nc, row, masked, want_pot, nslow))) return st;
     if (fixed)   // the root goes with level 1
         for (int l = 1; l <= std::max(1, nlev - 1); ++l)
             launch_l2l_fixed<T>(c, t, l == 1 ? 0 : c->level_begin[l], c->level_begin[std::min(l, nlev - 1) + 1], p, ncp, ncls,
@@ -1177,27 +1176,6 @@ tg_status fmm_eval(tg_ctx *c, int n, const double *pos, int64_t stride, const in
     return cuda_check(c, cudaGetLastError(), "fmm scatter");
 }
 
-// fast flags of the sorted particles as words, with a zero at n (the prefix sum then ends in its total)
-__global__ void fast_words(const uint8_t *fs, int n, uint32_t *w, const int *dn)
-{
-    n = dev_or(dn, n);
-    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i <= n; i += gridDim.x * blockDim.x) w[i] = i < n ? fs[i] : 0u;
-}
-
-tg_status fast_prefix(tg_ctx *c, const uint8_t *fs, int n, uint32_t **fpre, const DevEval *de)
-{
-    tg_status st;
-    uint32_t *w, *pre;
-    if ((st = ensure_t(c, B_FWORDS, (size_t)n + 1, &w)) || (st = ensure_t(c, B_FPRE, (size_t)n + 1, &pre))) return st;
-    {
-        ProfScope ps_(c, TG_K_M2L);
-        fast_words<<<grid_for((int64_t)n + 1, 256), 256, 0, c->stream>>>(fs, n, w, de ? &de->n : nullptr);
-    }
-    if ((st = exclusive_scan_u32(c, w, pre, n + 1, nullptr, de ? &de->np1 : nullptr))) return st;
-    *fpre = pre;
-    return TG_OK;
-}
-
 // zero rows[0] rows of `width` values (device row count)
 template <class T>
 __global__ void zero_rows_dev(T *p, const int *rows, int width)
@@ -1275,7 +1253,7 @@ static tg_status launch_p2p_dev_t(tg_ctx *c, const TreeView &t, const DevEval *d
                                   int stride)
 {
     (void)xyzm;
-    return launch_p2p_f32_dev(c, t, de, gp, wctr, p2p, cap_p2p, cap_cells, pf, nslow, acc4, stride, B_SCAN_TMP2);
+    return launch_p2p_f32_dev(c, t, de, gp, wctr, p2p, cap_p2p, cap_cells, pf, nslow, acc4, stride);
 }
 static tg_status launch_p2p_dev_t(tg_ctx *c, const TreeView &t, const DevEval *de, const Geom *gp,
                                   const unsigned long long *wctr, const uint2 *p2p, size_t cap_p2p, int cap_cells,
@@ -1284,7 +1262,7 @@ static tg_status launch_p2p_dev_t(tg_ctx *c, const TreeView &t, const DevEval *d
 {
     (void)gp;
     (void)pf;
-    return launch_p2p_f64_dev(c, t, de, wctr, p2p, cap_p2p, cap_cells, xyzm, nslow, acc4, stride, B_SCAN_TMP2);
+    return launch_p2p_f64_dev(c, t, de, wctr, p2p, cap_p2p, cap_cells, xyzm, nslow, acc4, stride);
 }
 
 template <class T, class T4>
@@ -1364,16 +1342,11 @@ static tg_status fmm_eval_dev_t(tg_ctx *c, DevEval *de, const BatchCaps &cap, co
     const int gcell = grid_for((int64_t)cap.cells * 32, 256);
     {
         ProfScope ps_(c, TG_K_TREE);
-        leaf_class_partition<<<gcell, 256, 0, c->stream>>>(t, xs, ys, zs, ms, fs, perm, xs2, ys2, zs2, ms2, fs2, perm2,
-                                                           nslow);
-    }
-    {
-        ProfScope ps_(c, TG_K_UP);
-        leaf_particles<T4><<<gcell, 256, 0, c->stream>>>(t, d_geom, xs2, ys2, zs2, ms2, pf, leaf_of);
+        leaf_class_partition<T4><<<gcell, 256, 0, c->stream>>>(t, d_geom, xs, ys, zs, ms, fs, perm, xs2, ys2, zs2, ms2, fs2,
+                                                               perm2, nslow, pf, leaf_of);
     }
     // P2P needs only the walk's lists and the leaf offsets, so it runs on the side stream (after the walk) beside
-    // the moments, M2L and the downward pass, into its own sums (acc4p, added by scatter_out); its scan takes
-    // its own scratch slot.  The forks and joins are events, which a stream capture turns into graph edges.
+    // the moments, M2L and the downward pass, into its own sums (acc4p, added by scatter_out).  The forks and joins are events, which a stream capture turns into graph edges.
     double *acc4p = nullptr;
     if ((st = ensure_t(c, B_ACC_P2P, (size_t)4 * cap.n, &acc4p))) {
         cudaStreamWaitEvent(c->stream, c->ev_walk, 0);
@@ -1384,10 +1357,6 @@ static tg_status fmm_eval_dev_t(tg_ctx *c, DevEval *de, const BatchCaps &cap, co
     {
         cudaStream_t main_stream = c->stream;
         c->stream = c->side;
-        {
-            ProfScope ps_(c, TG_K_OTHER);
-            zero_acc3<<<c->num_sms * 4, 256, 0, c->stream>>>(acc4p, cap.n, &de->n);
-        }
         const double *const xyzm[4] = {xs2, ys2, zs2, ms2};
         st = launch_p2p_dev_t(c, t, de, d_geom, wctr, p2p, cap.p2p, cap.cells, pf, xyzm, nslow, acc4p, cap.n);
         c->stream = main_stream;
@@ -1402,7 +1371,7 @@ static tg_status fmm_eval_dev_t(tg_ctx *c, DevEval *de, const BatchCaps &cap, co
         p2m_leaves<T, T4><<<grid_for((int64_t)cap.cells * 32, 128), 128, 0, c->stream>>>(
             t, d_geom, xs2, ys2, zs2, ms2, fs2, pf, p, nc, ncp, M, M01);
     }
-    for (int l = cap.levels - 1; l >= 0; --l) launch_m2m_fixed<T>(c, t, 0, 0, p, ncp, true, M, M01, de, l);
+    for (int l = cap.levels - 1; l >= 0; --l) launch_m2m_fixed<T>(c, t, 0, 0, p, ncp, true, M, M01, nslow, de, l);
     const bool harm = m2l_harmonic(c);
     const int ncpr = m2l_harmonic_row(p), row = harm ? ncpr : ncp;
     T *src = Ms, *dst = L;
@@ -1421,17 +1390,12 @@ static tg_status fmm_eval_dev_t(tg_ctx *c, DevEval *de, const BatchCaps &cap, co
         zero_rows_dev<T><<<c->num_sms * 4, 256, 0, c->stream>>>(dst, &de->rows, row);
     }
     cudaStreamWaitEvent(c->stream, c->ev_walk, 0);   // M2L reads the walk's blocks
-    uint32_t *fpre = nullptr;
-    st = fast_prefix(c, fs2, cap.n, &fpre, de);
-    if (!st) {
-        if (sizeof(T) == 4)
-            st = launch_m2l_f32_dev(c, t, de, d_geom, blocks, wctr + 1, (int64_t)cap.blocks,
-                                    reinterpret_cast<const float *>(src), reinterpret_cast<float *>(dst), p, row, cap.cells,
-                                    cap.m2l_src, fpre);
-        else
-            st = launch_m2l_f64_dev(c, t, de, d_geom, blocks, wctr + 1, (int64_t)cap.blocks,
-                                    reinterpret_cast<const double *>(src), reinterpret_cast<double *>(dst), p, row, fpre);
-    }
+    if (sizeof(T) == 4)
+        st = launch_m2l_f32_dev(c, t, de, d_geom, blocks, wctr + 1, (int64_t)cap.blocks, reinterpret_cast<const float *>(src),
+                                reinterpret_cast<float *>(dst), p, row, cap.cells, cap.m2l_src, nslow);
+    else
+        st = launch_m2l_f64_dev(c, t, de, d_geom, blocks, wctr + 1, (int64_t)cap.blocks, reinterpret_cast<const double *>(src),
+                                reinterpret_cast<double *>(dst), p, row, nslow);
     if (st) {
         cudaStreamWaitEvent(c->stream, c->ev_join, 0);   // no unjoined work on the side stream
         return st;

@@ -80,7 +80,7 @@ static void m2l_directed_launch(tg_ctx *c, const TreeView &t, const uint32_t *of
 // Harmonic set (G = -1/|d|, P <= 6): Mr and Lr hold the reduced coefficients, Lr starts at zero.
 template <int P>
 static tg_status m2l_f32_harmonic(tg_ctx *c, const TreeView &t, const M2LBlock *blocks, int64_t nblocks, const float *Mr,
-                                  float *Lr, int ncpr, bool masked, bool pot, int grid, const uint32_t *fpre)
+                                  float *Lr, int ncpr, bool masked, bool pot, int grid, const int32_t *nslow)
 {
     tg_status st;
     if (c->tune.m2l_form == 1) {
@@ -104,7 +104,7 @@ static tg_status m2l_f32_harmonic(tg_ctx *c, const TreeView &t, const M2LBlock *
 #define TG_M2L_H(MK, PT)                                                                                          \
     do {                                                                                                          \
         m2l_blocks_f32<G, MK, PT><<<grid, 128, 0, c->stream>>>(t, part, nblocks, pcnt, Mr, Lr, ncpr, 0.f, 0, nullptr, \
-                                                               nullptr, 0.0, fpre, c->d_counters + 11);            \
+                                                               nullptr, 0.0, nslow, c->d_counters + 11);            \
     } while (0)
     if (masked) {
         if (pot) TG_M2L_H(true, true);
@@ -118,7 +118,7 @@ static tg_status m2l_f32_harmonic(tg_ctx *c, const TreeView &t, const M2LBlock *
 }
 
 tg_status launch_m2l_f32(tg_ctx *c, const TreeView &t, const M2LBlock *blocks, int64_t nblocks, const float *Ms,
-                         float *L, int p, int nc, int ncp, bool masked, bool pot, const uint32_t *fpre)
+                         float *L, int p, int nc, int ncp, bool masked, bool pot, const int32_t *nslow)
 {
     const int plummer = c->prm.kernel == TG_KERNEL_PLUMMER;
     const float eoL = (float)ldexp(c->prm.eps, -c->walk_log2L);
@@ -126,12 +126,12 @@ tg_status launch_m2l_f32(tg_ctx *c, const TreeView &t, const M2LBlock *blocks, i
     const int grid = grid_for(nblocks * 32, 128, c->num_sms * c->tune.m2l_blocks_per_sm);
     if (m2l_harmonic(c)) {
         switch (p) {
-        case 1: return m2l_f32_harmonic<1>(c, t, blocks, nblocks, Ms, L, ncp, masked, pot, grid, fpre);
-        case 2: return m2l_f32_harmonic<2>(c, t, blocks, nblocks, Ms, L, ncp, masked, pot, grid, fpre);
-        case 3: return m2l_f32_harmonic<3>(c, t, blocks, nblocks, Ms, L, ncp, masked, pot, grid, fpre);
-        case 4: return m2l_f32_harmonic<4>(c, t, blocks, nblocks, Ms, L, ncp, masked, pot, grid, fpre);
-        case 5: return m2l_f32_harmonic<5>(c, t, blocks, nblocks, Ms, L, ncp, masked, pot, grid, fpre);
-        default: return m2l_f32_harmonic<6>(c, t, blocks, nblocks, Ms, L, ncp, masked, pot, grid, fpre);
+        case 1: return m2l_f32_harmonic<1>(c, t, blocks, nblocks, Ms, L, ncp, masked, pot, grid, nslow);
+        case 2: return m2l_f32_harmonic<2>(c, t, blocks, nblocks, Ms, L, ncp, masked, pot, grid, nslow);
+        case 3: return m2l_f32_harmonic<3>(c, t, blocks, nblocks, Ms, L, ncp, masked, pot, grid, nslow);
+        case 4: return m2l_f32_harmonic<4>(c, t, blocks, nblocks, Ms, L, ncp, masked, pot, grid, nslow);
+        case 5: return m2l_f32_harmonic<5>(c, t, blocks, nblocks, Ms, L, ncp, masked, pot, grid, nslow);
+        default: return m2l_f32_harmonic<6>(c, t, blocks, nblocks, Ms, L, ncp, masked, pot, grid, nslow);
         }
     }
     M2LBlock *part = nullptr;
@@ -144,7 +144,7 @@ tg_status launch_m2l_f32(tg_ctx *c, const TreeView &t, const M2LBlock *blocks, i
 #define TG_M2L_F32_(PP, MK, PT)                                                                                   \
     do {                                                                                                          \
         m2l_blocks_f32<M2LFull<PP>, MK, PT><<<grid, 128, 0, c->stream>>>(t, part, nblocks, pcnt, Ms, L, ncp, eoL,  \
-                                                                         plummer, nullptr, nullptr, 0.0, fpre,      \
+                                                                         plummer, nullptr, nullptr, 0.0, nslow,      \
                                                                          c->d_counters + 11);                       \
     } while (0)
 #define TG_M2L_F32(PP)                                                                                            \
@@ -181,7 +181,7 @@ __global__ void m2l_list_check(const uint32_t *off, const uint32_t *cnt, DevEval
 template <int P>
 static tg_status m2l_f32_dev_p(tg_ctx *c, const TreeView &t, const DevEval *de, const Geom *gp, const M2LBlock *blocks,
                                const unsigned long long *dnb, int64_t cap_blocks, const float *Ms, float *L, int ncp,
-                               int cap_cells, int grid, size_t cap_src, const uint32_t *fpre)
+                               int cap_cells, int grid, size_t cap_src, const int32_t *nslow)
 {
     const bool harm = m2l_harmonic(c);
     tg_status st;
@@ -205,7 +205,7 @@ static tg_status m2l_f32_dev_p(tg_ctx *c, const TreeView &t, const DevEval *de, 
     // the launch for the other class count returns at once
 #define TG_M2L_DEV(G, MK) \
     m2l_blocks_f32<G, MK, false><<<grid, 128, 0, c->stream>>>(t, part, cap_blocks, pcnt, Ms, L, ncp, 0.f, !harm, de, gp, \
-                                                              c->prm.eps, fpre, c->d_counters + 11)
+                                                              c->prm.eps, nslow, c->d_counters + 11)
     if (harm) {
         TG_M2L_DEV(M2LHarm<P>, true);
         TG_M2L_DEV(M2LHarm<P>, false);
@@ -219,14 +219,14 @@ static tg_status m2l_f32_dev_p(tg_ctx *c, const TreeView &t, const DevEval *de, 
 
 tg_status launch_m2l_f32_dev(tg_ctx *c, const TreeView &t, const DevEval *de, const Geom *gp, const M2LBlock *blocks,
                              const unsigned long long *dnb, int64_t cap_blocks, const float *Ms, float *L, int p,
-                             int ncp, int cap_cells, size_t cap_src, const uint32_t *fpre)
+                             int ncp, int cap_cells, size_t cap_src, const int32_t *nslow)
 {
     const int grid = c->num_sms * c->tune.m2l_blocks_per_sm;
     tg_status st;
     switch (p) {
-    case 4: st = m2l_f32_dev_p<4>(c, t, de, gp, blocks, dnb, cap_blocks, Ms, L, ncp, cap_cells, grid, cap_src, fpre); break;
-    case 5: st = m2l_f32_dev_p<5>(c, t, de, gp, blocks, dnb, cap_blocks, Ms, L, ncp, cap_cells, grid, cap_src, fpre); break;
-    case 6: st = m2l_f32_dev_p<6>(c, t, de, gp, blocks, dnb, cap_blocks, Ms, L, ncp, cap_cells, grid, cap_src, fpre); break;
+    case 4: st = m2l_f32_dev_p<4>(c, t, de, gp, blocks, dnb, cap_blocks, Ms, L, ncp, cap_cells, grid, cap_src, nslow); break;
+    case 5: st = m2l_f32_dev_p<5>(c, t, de, gp, blocks, dnb, cap_blocks, Ms, L, ncp, cap_cells, grid, cap_src, nslow); break;
+    case 6: st = m2l_f32_dev_p<6>(c, t, de, gp, blocks, dnb, cap_blocks, Ms, L, ncp, cap_cells, grid, cap_src, nslow); break;
     default: return set_err(c, TG_ERR_ARG, "batched M2L needs 4 <= p <= 6");
     }
     if (st) return st;
@@ -237,7 +237,7 @@ tg_status launch_m2l_f32_dev(tg_ctx *c, const TreeView &t, const DevEval *de, co
 // then a capacity, and the launch for the other class count returns).
 template <int P>
 static tg_status m2l_f64_p(tg_ctx *c, const TreeView &t, const M2LBlock *blocks, int64_t nb, const double *Ms, double *L,
-                           int ncp, bool masked, bool pot, const uint32_t *fpre, const DevEval *de, const Geom *gp,
+                           int ncp, bool masked, bool pot, const int32_t *nslow, const DevEval *de, const Geom *gp,
                            const unsigned long long *dnb)
 {
     const bool harm = m2l_harmonic(c);
@@ -245,7 +245,7 @@ static tg_status m2l_f64_p(tg_ctx *c, const TreeView &t, const M2LBlock *blocks,
     const int grid = c->num_sms * 4;
     ProfScope ps_(c, TG_K_M2L);
 #define TG_M2L64_(G, MK, PT)                                                                                       \
-    m2l_pairs_f64<G, MK, PT><<<grid, 128, 0, c->stream>>>(t, blocks, nb, dnb, Ms, L, ncp, eoL, !harm, de, gp, c->prm.eps, fpre)
+    m2l_pairs_f64<G, MK, PT><<<grid, 128, 0, c->stream>>>(t, blocks, nb, dnb, Ms, L, ncp, eoL, !harm, de, gp, c->prm.eps, nslow)
 #define TG_M2L64(MK, PT)                                                                                           \
     do {                                                                                                           \
         if (harm) TG_M2L64_(M2LHarm<P>, MK, PT);                                                                   \
@@ -267,32 +267,32 @@ static tg_status m2l_f64_p(tg_ctx *c, const TreeView &t, const M2LBlock *blocks,
 }
 
 static tg_status m2l_f64_any(tg_ctx *c, const TreeView &t, const M2LBlock *blocks, int64_t nb, const double *Ms, double *L,
-                             int p, int ncp, bool masked, bool pot, const uint32_t *fpre, const DevEval *de,
+                             int p, int ncp, bool masked, bool pot, const int32_t *nslow, const DevEval *de,
                              const Geom *gp, const unsigned long long *dnb)
 {
     switch (p) {
-    case 1: return m2l_f64_p<1>(c, t, blocks, nb, Ms, L, ncp, masked, pot, fpre, de, gp, dnb);
-    case 2: return m2l_f64_p<2>(c, t, blocks, nb, Ms, L, ncp, masked, pot, fpre, de, gp, dnb);
-    case 3: return m2l_f64_p<3>(c, t, blocks, nb, Ms, L, ncp, masked, pot, fpre, de, gp, dnb);
-    case 4: return m2l_f64_p<4>(c, t, blocks, nb, Ms, L, ncp, masked, pot, fpre, de, gp, dnb);
-    case 5: return m2l_f64_p<5>(c, t, blocks, nb, Ms, L, ncp, masked, pot, fpre, de, gp, dnb);
-    default: return m2l_f64_p<6>(c, t, blocks, nb, Ms, L, ncp, masked, pot, fpre, de, gp, dnb);
+    case 1: return m2l_f64_p<1>(c, t, blocks, nb, Ms, L, ncp, masked, pot, nslow, de, gp, dnb);
+    case 2: return m2l_f64_p<2>(c, t, blocks, nb, Ms, L, ncp, masked, pot, nslow, de, gp, dnb);
+    case 3: return m2l_f64_p<3>(c, t, blocks, nb, Ms, L, ncp, masked, pot, nslow, de, gp, dnb);
+    case 4: return m2l_f64_p<4>(c, t, blocks, nb, Ms, L, ncp, masked, pot, nslow, de, gp, dnb);
+    case 5: return m2l_f64_p<5>(c, t, blocks, nb, Ms, L, ncp, masked, pot, nslow, de, gp, dnb);
+    default: return m2l_f64_p<6>(c, t, blocks, nb, Ms, L, ncp, masked, pot, nslow, de, gp, dnb);
     }
 }
 
 tg_status launch_m2l_f64_dev(tg_ctx *c, const TreeView &t, const DevEval *de, const Geom *gp, const M2LBlock *blocks,
                              const unsigned long long *dnb, int64_t cap_blocks, const double *Ms, double *L, int p,
-                             int ncp, const uint32_t *fpre)
+                             int ncp, const int32_t *nslow)
 {
     if (p < 1 || p > 6) return set_err(c, TG_ERR_ARG, "batched M2L needs 1 <= p <= 6");
-    return m2l_f64_any(c, t, blocks, cap_blocks, Ms, L, p, ncp, true, false, fpre, de, gp, dnb);
+    return m2l_f64_any(c, t, blocks, cap_blocks, Ms, L, p, ncp, true, false, nslow, de, gp, dnb);
 }
 
 tg_status launch_m2l_f64(tg_ctx *c, const TreeView &t, const M2LBlock *blocks, int64_t nblocks, const double *Ms,
-                         double *L, int p, int nc, int ncp, bool masked, bool pot, const uint32_t *fpre)
+                         double *L, int p, int nc, int ncp, bool masked, bool pot, const int32_t *nslow)
 {
     if (p > TG_PMAX) return launch_m2l_hi<double>(c, t, blocks, nblocks, Ms, L, p, nc, ncp, masked, true);
-    if (p <= 6) return m2l_f64_any(c, t, blocks, nblocks, Ms, L, p, ncp, masked, pot, fpre, nullptr, nullptr, nullptr);
+    if (p <= 6) return m2l_f64_any(c, t, blocks, nblocks, Ms, L, p, ncp, masked, pot, nslow, nullptr, nullptr, nullptr);
     const int plummer = c->prm.kernel == TG_KERNEL_PLUMMER;
     const double eoL = ldexp(c->prm.eps, -c->walk_log2L);
     const int grid = grid_for(nblocks * 32, 128, c->num_sms * 16);

@@ -150,7 +150,7 @@ static __global__ void m2l_partition(const M2LBlock *__restrict__ in, int64_t nb
 // blocks at the end of part, four per packed round (see m2l_partition).
 // Batched path (de non-null): the class count and the root cube come from the device; the launch for
 // the other class count returns at once.
-// Kick pairs (MASKED) with fpre (the prefix sum of the fast flags over the sorted particles): a target
+// Kick pairs (MASKED) with nslow (the slow particles of every cell): a target
 // cell needs the all-sources local (class 0) only if it holds slow particles, and the slow-sources local
 // (class 1) only if it holds fast particles, and a class-1 contraction adds something only if its source
 // holds slow particles (class 1 carries the slow masses); a round skips a side's contraction of a class
@@ -162,7 +162,7 @@ __global__ void __launch_bounds__(128) m2l_blocks_f32(TreeView t, const M2LBlock
                                                       const unsigned long long *__restrict__ pcnt,
                                                       const float *__restrict__ Ms, float *L, int ncp, float eps_over_L,
                                                       int plummer, const DevEval *de, const Geom *gp, double eps,
-                                                      const uint32_t *__restrict__ fpre, unsigned long long *class_ctr)
+                                                      const int32_t *__restrict__ nslow, unsigned long long *class_ctr)
 {
     unsigned long long my_sc = 0;   // side contractions the method needs: (pair side, class) with a target
     if (de) {
@@ -226,14 +226,13 @@ __global__ void __launch_bounds__(128) m2l_blocks_f32(TreeView t, const M2LBlock
             // holds the slow masses only: a source without slow particles has zero class-1 moments, so
             // its class-1 contraction adds nothing and is left out with the others of the round.
             unsigned need = 0xfu;   // bit cls: side a needs class cls; bit 2 + cls: side b does
-            if (MASKED && fpre) {
+            if (MASKED && nslow) {
                 int fx = 0, sx = 0, fy = 0, sy = 0;
                 if (active) {
-                    const int ax = t.first[x], ay = t.first[y];
-                    fx = (int)(fpre[ax + t.count[x]] - fpre[ax]);
-                    sx = t.count[x] - fx;
-                    fy = (int)(fpre[ay + t.count[y]] - fpre[ay]);
-                    sy = t.count[y] - fy;
+                    sx = nslow[x];
+                    fx = t.count[x] - sx;
+                    sy = nslow[y];
+                    fy = t.count[y] - sy;
                 }
                 const bool a1 = fx > 0 && sy > 0, b1 = fy > 0 && sx > 0;
                 need = (__any_sync(0xffffffffu, sx > 0) ? 1u : 0u) | (__any_sync(0xffffffffu, a1) ? 2u : 0u) |
@@ -465,7 +464,7 @@ __global__ void __launch_bounds__(128) m2l_pairs_f64(TreeView t, const M2LBlock 
                                                      const unsigned long long *dnb, const double *__restrict__ Ms,
                                                      double *L, int ncp, double eps_over_L, int plummer,
                                                      const DevEval *de, const Geom *gp, double eps,
-                                                     const uint32_t *__restrict__ fpre)
+                                                     const int32_t *__restrict__ nslow)
 {
     if (de) {   // batched path: classes, count and root cube on the device
         if ((de->masked != 0) != MASKED) return;
@@ -521,14 +520,13 @@ __global__ void __launch_bounds__(128) m2l_pairs_f64(TreeView t, const M2LBlock 
                 ly = bg.ly;
             }
             unsigned need = 0xfu;   // bit cls: side x needs class cls; bit 2 + cls: side y does
-            if (MASKED && fpre) {
+            if (MASKED && nslow) {
                 int fx = 0, sx = 0, fy = 0, sy = 0;
                 if (active) {
-                    const int ax = t.first[x], ay = t.first[y];
-                    fx = (int)(fpre[ax + t.count[x]] - fpre[ax]);
-                    sx = t.count[x] - fx;
-                    fy = (int)(fpre[ay + t.count[y]] - fpre[ay]);
-                    sy = t.count[y] - fy;
+                    sx = nslow[x];
+                    fx = t.count[x] - sx;
+                    sy = nslow[y];
+                    fy = t.count[y] - sy;
                 }
                 need = (__any_sync(0xffffffffu, sx > 0) ? 1u : 0u) | (__any_sync(0xffffffffu, fx > 0 && sy > 0) ? 2u : 0u) |
                        (__any_sync(0xffffffffu, sy > 0) ? 4u : 0u) | (__any_sync(0xffffffffu, fy > 0 && sx > 0) ? 8u : 0u);

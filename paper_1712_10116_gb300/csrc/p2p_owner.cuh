@@ -63,6 +63,37 @@ __global__ void p2p_owner_count(const uint2 *__restrict__ pairs, int64_t npairs,
     }
 }
 
+// Room for every owner's partners: any place will do, so warps reserve it with one atomic on ctr[2].
+__global__ void p2p_owner_place(const uint32_t *__restrict__ cnt, uint32_t *off, int ncell, const int *dn, uint32_t *ctr)
+{
+    ncell = dev_or(dn, ncell);
+    const int lane = threadIdx.x & 31, stride = gridDim.x * blockDim.x;
+    for (int c0 = blockIdx.x * blockDim.x; c0 < ncell; c0 += stride) {   // whole warps iterate together
+        const int c = c0 + threadIdx.x;
+        const uint32_t n = c < ncell ? cnt[c] : 0u;
+        uint32_t incl = n;
+#pragma unroll
+        for (int d = 1; d < 32; d <<= 1) {
+            const uint32_t y = __shfl_up_sync(0xffffffffu, incl, d);
+            if (lane >= d) incl += y;
+        }
+        uint32_t base = 0u;
+        if (lane == 31 && incl) base = atomicAdd(&ctr[2], incl);
+        base = __shfl_sync(0xffffffffu, base, 31);
+        if (c < ncell) off[c] = base + incl - n;
+    }
+}
+
+// Batched path: everything the P2P adds to, cleared in one launch (counts and fills of the cells, the three counters
+// behind them, the acceleration sums).
+__global__ void p2p_clear(const DevEval *de, uint32_t *cnt, uint32_t *fill, uint32_t *ctr, double *acc4, int64_t stride4)
+{
+    const int tid = blockIdx.x * blockDim.x + threadIdx.x, nt = gridDim.x * blockDim.x;
+    for (int i = tid; i < de->ncell; i += nt) cnt[i] = fill[i] = 0u;
+    if (tid < 3) ctr[tid] = 0u;
+    for (int i = tid; i < de->n; i += nt) acc4[i] = acc4[stride4 + i] = acc4[2 * stride4 + i] = 0.0;
+}
+
 // Partners grouped by owner: partners[own_off[B] .. own_off[B] + own_cnt[B]).  Every own_unit-th
 // partner of an owner also opens a work unit (owner, position); ctr[0] counts the units.
 // own_fill and ctr start at zero.  Lanes with equal owners take consecutive slots with one atomic, and
@@ -494,17 +525,10 @@ static int owner_occupancy(int rows)
     return occ[rows];
 }
 
-// zero n32[0] + extra words at p (n32: a device count, nullable; the batched path cannot size a memset)
-__global__ void zero_u32_dev(uint32_t *p, const int *n32, int extra)
-{
-    const int n = (n32 ? *n32 : 0) + extra;
-    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) p[i] = 0u;
-}
-
 // The distinct leaf pairs grouped by owner (both precisions).
 struct OwnerLists {
     uint2 *units = nullptr;
-    uint32_t *ctr = nullptr, *off = nullptr, *cnt = nullptr;   // ctr: [0] work units, [1] next unit to take
+    uint32_t *ctr = nullptr, *off = nullptr, *cnt = nullptr;   // ctr: [0] units, [1] next to take, [2] partners placed
     int32_t *partners = nullptr;
 };
 
@@ -515,19 +539,22 @@ static tg_status owner_lists(tg_ctx *c, const TreeView &t, const uint2 *pairs, i
     uint32_t *own_fill;
     uint2 *tagged;
     const int64_t max_units = own_max_units(npairs, ncell);
-    if ((st = ensure_t(c, B_OWN_CNT, (size_t)ncell + 2, &o->cnt)) || (st = ensure_t(c, B_OWN_FILL, ncell, &own_fill)) ||
+    if ((st = ensure_t(c, B_OWN_CNT, (size_t)ncell + 3, &o->cnt)) || (st = ensure_t(c, B_OWN_FILL, ncell, &own_fill)) ||
         (st = ensure_t(c, B_OWN_OFF, ncell, &o->off)) || (st = ensure_t(c, B_OWN_LIST, max_units, &o->units)) ||
         (st = ensure_t(c, B_OWN_TAG, npairs, &tagged)) || (st = ensure_t(c, B_OWN_PART, npairs, &o->partners)))
         return st;
     o->ctr = o->cnt + ncell;
-    cudaMemsetAsync(o->cnt, 0, sizeof(uint32_t) * ((size_t)ncell + 2), c->stream);
+    cudaMemsetAsync(o->cnt, 0, sizeof(uint32_t) * ((size_t)ncell + 3), c->stream);
     cudaMemsetAsync(own_fill, 0, sizeof(uint32_t) * (size_t)ncell, c->stream);
     if (npairs > 0) {
         {
             ProfScope ps_(c, TG_K_OTHER);
             p2p_owner_count<<<grid_for(npairs, 256), 256, 0, c->stream>>>(pairs, npairs, t.count, o->cnt, tagged, nullptr);
         }
-        if ((st = exclusive_scan_u32(c, o->cnt, o->off, ncell, nullptr))) return st;
+        {
+            ProfScope ps_(c, TG_K_OTHER);
+            p2p_owner_place<<<grid_for(ncell, 256), 256, 0, c->stream>>>(o->cnt, o->off, ncell, nullptr, o->ctr);
+        }
         {
             ProfScope ps_(c, TG_K_OTHER);
             p2p_owner_fill<<<grid_for(npairs, 256), 256, 0, c->stream>>>(tagged, npairs, o->off, own_fill, o->partners,
@@ -540,15 +567,15 @@ static tg_status owner_lists(tg_ctx *c, const TreeView &t, const uint2 *pairs, i
 // The same with every size on the device (batched HOLD step): the pair count comes from the walk's counters, the
 // cell count from de; buffers are sized for the capacities.
 static tg_status owner_lists_dev(tg_ctx *c, const TreeView &t, const DevEval *de, const unsigned long long *walk_ctr,
-                                 const uint2 *p2p, size_t cap_p2p, int cap_cells, int scan_scratch, bool f64,
+                                 const uint2 *p2p, size_t cap_p2p, int cap_cells, bool f64, double *acc4, int stride,
                                  OwnerLists *o)
 {
     tg_status st;
     uint32_t *own_fill;
     uint2 *tagged;
     const int64_t max_units = own_max_units((int64_t)cap_p2p, cap_cells);
-    if ((st = ensure_t(c, B_OWN_CNT, (size_t)cap_cells + 2, &o->cnt)) ||
-        (st = ensure_t(c, B_OWN_FILL, (size_t)cap_cells + 2, &own_fill)) ||
+    if ((st = ensure_t(c, B_OWN_CNT, (size_t)cap_cells, &o->cnt)) ||
+        (st = ensure_t(c, B_OWN_FILL, (size_t)cap_cells + 3, &own_fill)) ||
         (st = ensure_t(c, B_OWN_OFF, (size_t)cap_cells, &o->off)) || (st = ensure_t(c, B_OWN_LIST, max_units, &o->units)) ||
         (st = ensure_t(c, B_OWN_TAG, cap_p2p, &tagged)) || (st = ensure_t(c, B_OWN_PART, cap_p2p, &o->partners)))
         return st;
@@ -556,14 +583,12 @@ static tg_status owner_lists_dev(tg_ctx *c, const TreeView &t, const DevEval *de
     const int g = c->num_sms * 4;
     {
         ProfScope ps_(c, TG_K_OTHER);
-        zero_u32_dev<<<g, 256, 0, c->stream>>>(o->cnt, &de->ncell, 0);
-        zero_u32_dev<<<g, 256, 0, c->stream>>>(own_fill, &de->ncell, 0);
-        zero_u32_dev<<<1, 32, 0, c->stream>>>(o->ctr, nullptr, 2);
+        p2p_clear<<<g, 256, 0, c->stream>>>(de, o->cnt, own_fill, o->ctr, acc4, stride);
         p2p_owner_count<<<g, 256, 0, c->stream>>>(p2p, (int64_t)cap_p2p, t.count, o->cnt, tagged, walk_ctr + 2);
     }
-    if ((st = exclusive_scan_u32(c, o->cnt, o->off, cap_cells, nullptr, &de->ncell, scan_scratch))) return st;
     {
         ProfScope ps_(c, TG_K_OTHER);
+        p2p_owner_place<<<g, 256, 0, c->stream>>>(o->cnt, o->off, cap_cells, &de->ncell, o->ctr);
         p2p_owner_fill<<<g, 256, 0, c->stream>>>(tagged, (int64_t)cap_p2p, o->off, own_fill, o->partners, o->units, o->ctr,
                                                   walk_ctr + 2, f64);
     }
@@ -612,10 +637,10 @@ tg_status launch_p2p_f32(tg_ctx *c, const TreeView &t, const uint2 *pairs, int64
 // come from the walk's counters, the cell count from de; buffers are sized for the capacities.
 tg_status launch_p2p_f32_dev(tg_ctx *c, const TreeView &t, const DevEval *de, const Geom *gp,
                              const unsigned long long *walk_ctr, const uint2 *p2p, size_t cap_p2p, int cap_cells,
-                             const float4 *pf, const int32_t *nslow, double *acc4, int stride, int scan_scratch)
+                             const float4 *pf, const int32_t *nslow, double *acc4, int stride)
 {
     OwnerLists o;
-    tg_status st = owner_lists_dev(c, t, de, walk_ctr, p2p, cap_p2p, cap_cells, scan_scratch, false, &o);
+    tg_status st = owner_lists_dev(c, t, de, walk_ctr, p2p, cap_p2p, cap_cells, false, acc4, stride, &o);
     if (st) return st;
     const float eps = (float)c->prm.eps;
     unsigned long long *pc = c->d_counters;

@@ -361,10 +361,10 @@ tg_status launch_p2p_f64(tg_ctx *c, const TreeView &t, const uint2 *pairs, int64
 
 tg_status launch_p2p_f64_dev(tg_ctx *c, const TreeView &t, const DevEval *de, const unsigned long long *walk_ctr,
                              const uint2 *p2p, size_t cap_p2p, int cap_cells, const double *const xyzm[4],
-                             const int32_t *nslow, double *acc4, int stride, int scan_scratch)
+                             const int32_t *nslow, double *acc4, int stride)
 {
     OwnerLists o;
-    tg_status st = owner_lists_dev(c, t, de, walk_ctr, p2p, cap_p2p, cap_cells, scan_scratch, true, &o);
+    tg_status st = owner_lists_dev(c, t, de, walk_ctr, p2p, cap_p2p, cap_cells, true, acc4, stride, &o);
     if (st) return st;
     const Bodies pf{xyzm[0], xyzm[1], xyzm[2], xyzm[3]};
     return launch_owner_f64(c, t, o, 0, nullptr, 0, pf, nslow, false, acc4, stride, walk_ctr, p2p, cap_p2p);

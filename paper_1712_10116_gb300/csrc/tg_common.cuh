@@ -53,7 +53,6 @@ struct DevEval {
     int ncell;              // cells of the tree
     int nlev;               // levels of the tree
     int rows;               // 2 * ncell (expansion rows, both classes)
-    int np1;                // n + 1 (prefix sum of the fast flags, with its total)
     uint32_t overflow;      // bit 0: cells, bit 1: levels, bit 2: walk lists (the step must be redone); bit 3:
                             // a bounded wait of the sort ran out
     int level_begin[kMaxLevel + 3];   // first cell of each level; [nlev] = ncell
@@ -152,7 +151,7 @@ enum Slot {
     B_HHS_SCAN, B_HHS_TMP, B_RED, B_DIAG_POT, B_DIAG_ACC,
     B_OWN_CNT, B_OWN_FILL, B_OWN_OFF, B_OWN_LIST, B_OWN_TAG, B_OWN_PART, B_SNAP, B_TUNE_ACC,
     B_MACP, B_DEVEVAL, B_HOLD, B_FRAME_X, B_FRAME_M, B_FRAME_F, B_SPLIT_FLAG, B_SPLIT_PRE,
-    B_M2L_CNT, B_M2L_OFF, B_M2L_FILL, B_M2L_SRC, B_FWORDS, B_FPRE, B_M2L_PART, B_M2L_PCNT, B_TUNE_SNAP, B_SCAN_TMP2, B_ACC_P2P,
+    B_M2L_CNT, B_M2L_OFF, B_M2L_FILL, B_M2L_SRC, B_M2L_PART, B_M2L_PCNT, B_TUNE_SNAP, B_ACC_P2P,
     B_LAST_SLOT
 };
 static_assert(B_LAST_SLOT <= kMaxSlots, "tg_ctx::buf holds fewer entries than there are slots");
@@ -227,13 +226,13 @@ tg_status injected_alloc_failure(tg_ctx *c, size_t bytes, int slot);
 
 // Device-wide exclusive scan of uint32 (in place allowed); optional total to a device word.
 tg_status exclusive_scan_u32(tg_ctx *c, const uint32_t *in, uint32_t *out, int n, uint32_t *d_total,
-                             const int *dn = nullptr, int scratch = B_SCAN_TMP);
+                             const int *dn = nullptr);
 
 // ---- translate.cu: M2M and L2L of one level at orders up to 6, and the moments the harmonic M2L reads.  With de the
 // level range and the classes come from the device.  Lr: harmonic M2L sums (null: L holds the full set's).
 template <class T>
 void launch_m2m_fixed(tg_ctx *c, const TreeView &t, int lb, int le, int p, int ncp, bool masked, T *M, double *M01,
-                      const DevEval *de, int lvl);
+                      int32_t *nslow, const DevEval *de, int lvl);
 template <class T>
 void launch_l2l_fixed(tg_ctx *c, const TreeView &t, int lb, int le, int p, int ncp, int ncls, T *L, const T *Lr, int ncpr,
                       const DevEval *de, int lvl);
@@ -246,33 +245,30 @@ inline bool m2l_harmonic(const tg_ctx *c) { return c->prm.kernel != TG_KERNEL_PL
 inline int m2l_harmonic_row(int p) { return ((p + 1) * (p + 1) + 3) & ~3; }
 
 // ---- m2l.cu: mutual M2L of the walk's blocks into L (normalised expansions).  pot = false: the
-// float32 kernels leave out the potential term L^0.  fpre (kick pairs, nullable): prefix sum of the fast
-// flags of the sorted particles, so that contractions no target needs are skipped.
+// float32 kernels leave out the potential term L^0.  nslow (kick pairs, nullable): slow particles of every cell,
+// so that contractions no target needs are skipped.
 tg_status launch_m2l_f32(tg_ctx *c, const TreeView &t, const M2LBlock *blocks, int64_t nblocks, const float *Ms,
-                         float *L, int p, int nc, int ncp, bool masked, bool pot, const uint32_t *fpre = nullptr);
-// the prefix sum of the fast flags fs of n sorted particles (n + 1 entries) into fpre (dn: device n)
-tg_status fast_prefix(tg_ctx *c, const uint8_t *fs, int n, uint32_t **fpre, const DevEval *de);
+                         float *L, int p, int nc, int ncp, bool masked, bool pot, const int32_t *nslow = nullptr);
 tg_status launch_m2l_f32_dev(tg_ctx *c, const TreeView &t, const DevEval *de, const Geom *gp, const M2LBlock *blocks,
                              const unsigned long long *dnb, int64_t cap_blocks, const float *Ms, float *L, int p,
-                             int ncp, int cap_cells, size_t cap_src, const uint32_t *fpre);
+                             int ncp, int cap_cells, size_t cap_src, const int32_t *nslow);
 tg_status launch_m2l_f64_dev(tg_ctx *c, const TreeView &t, const DevEval *de, const Geom *gp, const M2LBlock *blocks,
                              const unsigned long long *dnb, int64_t cap_blocks, const double *Ms, double *L, int p,
-                             int ncp, const uint32_t *fpre);
+                             int ncp, const int32_t *nslow);
 tg_status launch_m2l_f64(tg_ctx *c, const TreeView &t, const M2LBlock *blocks, int64_t nblocks, const double *Ms,
-                         double *L, int p, int nc, int ncp, bool masked, bool pot, const uint32_t *fpre);
+                         double *L, int p, int nc, int ncp, bool masked, bool pot, const int32_t *nslow);
 // ---- p2p.cu: mutual P2P of all leaf pairs (distinct pairs and self pairs) into acc4.
 tg_status launch_p2p_f32(tg_ctx *c, const TreeView &t, const uint2 *pairs, int64_t npairs, const uint2 *self_pairs,
                          int64_t nself, const float4 *pf, const int32_t *nslow, bool pot, double *acc4);
 tg_status launch_p2p_f32_dev(tg_ctx *c, const TreeView &t, const DevEval *de, const Geom *gp,
                              const unsigned long long *walk_ctr, const uint2 *p2p, size_t cap_p2p, int cap_cells,
-                             const float4 *pf, const int32_t *nslow, double *acc4, int stride,
-                             int scan_scratch = B_SCAN_TMP);
+                             const float4 *pf, const int32_t *nslow, double *acc4, int stride);
 // (float64: xyzm holds the sorted coordinates and masses)
 tg_status launch_p2p_f64(tg_ctx *c, const TreeView &t, const uint2 *pairs, int64_t npairs, const uint2 *self_pairs,
                          int64_t nself, const double *const xyzm[4], const int32_t *nslow, bool pot, double *acc4);
 tg_status launch_p2p_f64_dev(tg_ctx *c, const TreeView &t, const DevEval *de, const unsigned long long *walk_ctr,
                              const uint2 *p2p, size_t cap_p2p, int cap_cells, const double *const xyzm[4],
-                             const int32_t *nslow, double *acc4, int stride, int scan_scratch = B_SCAN_TMP);
+                             const int32_t *nslow, double *acc4, int stride);
 
 // The sort itself, also used by the allocation-free entry point (noalloc.cu).
 constexpr int kSortTileItems = 2048;     // items per radix-sort block (256 threads x 8)

@@ -52,10 +52,10 @@ __device__ __forceinline__ void shift_coef(bool neg, T (&c)[P + 1])
 // ------------------------------------------------------------------ M2M
 // M~_P^n = sum_children sum_{k <= n} C(n,k) 2^-(2|n-k| + |k|) (+-1)^(n-k) M~_c^k for the parents of one level.  The
 // monopole and dipole are summed in float64 (M01), every order also in T.  The fast class is left out when the
-// evaluation has no classes.
+// evaluation has no classes; with classes the slow particles of the children are counted too (nslow).
 template <int P, class T>
 __global__ void __launch_bounds__(128) m2m_fixed(TreeView t, int lb, int le, int masked, int ncp, T *M, double *M01,
-                                                 const DevEval *de, int lvl)
+                                                 int32_t *nslow, const DevEval *de, int lvl)
 {
     if (de) {   // level range and classes on the device (batched path); levels past the tree are empty
         if (lvl + 1 >= de->nlev) return;
@@ -109,7 +109,11 @@ __global__ void __launch_bounds__(128) m2m_fixed(TreeView t, int lb, int le, int
                     v[k] = keep + __shfl_xor_sync(0xffffffffu, send, h);
                 }
         }
+        int slow = nslow && child ? nslow[ch] : 0;
+#pragma unroll
+        for (int o = 1; o < 8; o <<= 1) slow += __shfl_xor_sync(0xffffffffu, slow, o);
         if (nch == 0) continue;
+        if (nslow && cls == 0 && q == 0) nslow[c] = slow;
         T *row = M + ((size_t)c * 2 + cls) * ncp;
         if (q < 4) {
             const double mine = q == 0 ? lo[0] : (q == 1 ? lo[1] : (q == 2 ? lo[2] : lo[3]));
@@ -239,11 +243,11 @@ __global__ void __launch_bounds__(128) m2l_moments_h(int ncell, int masked, cons
 
 template <class T>
 void launch_m2m_fixed(tg_ctx *c, const TreeView &t, int lb, int le, int p, int ncp, bool masked, T *M, double *M01,
-                      const DevEval *de, int lvl)
+                      int32_t *nslow, const DevEval *de, int lvl)
 {
     const int grid = de ? c->num_sms * 4 : grid_for((int64_t)(le - lb) * 8 * (masked ? 2 : 1), 128, c->num_sms * 8);
     ProfScope ps_(c, TG_K_UP);
-#define TG_CALL(PP) m2m_fixed<PP, T><<<grid, 128, 0, c->stream>>>(t, lb, le, masked, ncp, M, M01, de, lvl)
+#define TG_CALL(PP) m2m_fixed<PP, T><<<grid, 128, 0, c->stream>>>(t, lb, le, masked, ncp, M, M01, nslow, de, lvl)
     TG_BY_ORDER(TG_CALL)
 #undef TG_CALL
 }
@@ -273,7 +277,7 @@ void launch_m2l_moments(tg_ctx *c, int ncell, int p, int ncp, bool masked, const
 }
 
 #define TG_INST(T)                                                                                                      \
-    template void launch_m2m_fixed<T>(tg_ctx *, const TreeView &, int, int, int, int, bool, T *, double *, const DevEval *, int); \
+    template void launch_m2m_fixed<T>(tg_ctx *, const TreeView &, int, int, int, int, bool, T *, double *, int32_t *, const DevEval *, int); \
     template void launch_l2l_fixed<T>(tg_ctx *, const TreeView &, int, int, int, int, int, T *, const T *, int,          \
                                       const DevEval *, int);                                                            \
     template void launch_m2l_moments<T>(tg_ctx *, int, int, int, bool, const T *, const double *, T *, int, const DevEval *);
