@@ -341,13 +341,14 @@ tg_status tg_timesteps(tg_ctx *ctx, int64_t n, const double *a_old, const double
  *   cuda_stream  the cudaStream_t the work is enqueued on (NULL = legacy default stream)
  *
  * It allocates nothing (no cudaMalloc, cudaFree or allocating library call).  Its scratch is one
- * file-scope device array of about 6.3 MB that every GPU loading the library holds until the
+ * file-scope device array of about 6.8 MB that every GPU loading the library holds until the
  * process exits.  Every call looks up that array's device address (cudaGetSymbolAddress, which
  * allocates nothing) on the current device, so pos, keys_out and perm_out must be memory of the
  * current device (or managed memory).  All calls share the array, so two calls whose work
  * overlaps on the GPU (different streams, or host threads racing) corrupt each other's results:
  * serialise them.  Returns TG_ERR_ARG for bad sizes or for pointers that are not memory of the
- * current device, and TG_ERR_CUDA if a launch fails; the call is asynchronous otherwise. */
+ * current device, and TG_ERR_CUDA if a launch fails; the call is asynchronous otherwise.  A sort
+ * whose bounded device-side wait gives up leaves -1 in every entry of perm_out. */
 #define TG_NOALLOC_MAX_N 262144
 tg_status tg_morton_sort_noalloc(int64_t n, const double *pos, uint64_t *keys_out, int64_t *perm_out,
                                  void *cuda_stream);

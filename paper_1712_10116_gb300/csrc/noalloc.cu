@@ -51,11 +51,15 @@ tg_status scratch_for_current_device(unsigned char **out)
     return TG_OK;
 }
 
-__global__ void noalloc_export(int n, const uint64_t *keys, const uint32_t *vals, uint64_t *keys_out, int64_t *perm_out)
+// The call returns before the sort has run, so a sort whose bounded wait gave up cannot become a status: its
+// permutation is all -1 instead.
+__global__ void noalloc_export(int n, const uint64_t *keys, const uint32_t *vals, const uint32_t *flag, uint64_t *keys_out,
+                               int64_t *perm_out)
 {
+    const bool bad = *flag != 0;
     for (int64_t s = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; s < n; s += (int64_t)gridDim.x * blockDim.x) {
         keys_out[s] = keys[s];
-        perm_out[s] = (int64_t)vals[s];
+        perm_out[s] = bad ? -1 : (int64_t)vals[s];
     }
 }
 
@@ -94,10 +98,11 @@ extern "C" tg_status tg_morton_sort_noalloc(int64_t n, const double *pos, uint64
     if (cudaMemsetAsync(base + kOffSort, 0, 256, s) != cudaSuccess) return TG_ERR_CUDA;
     bool swapped, gathered;
     int launches;
-    if (launch_sort(s, ni, nullptr, pos, n, nullptr, nullptr, nullptr, geom, k0, k1, v0, v1, sort_scratch(base + kOffSort, n),
-                    SortedOut{}, &swapped, &gathered, &launches) != cudaSuccess)
+    const SortScratch ss = sort_scratch(base + kOffSort, n);
+    if (launch_sort(s, ni, nullptr, pos, n, nullptr, nullptr, nullptr, geom, k0, k1, v0, v1, ss, SortedOut{},
+                    &swapped, &gathered, &launches) != cudaSuccess)
         return TG_ERR_CUDA;
-    noalloc_export<<<grid_for(n, 256), 256, 0, s>>>(ni, swapped ? k1 : k0, swapped ? v1 : v0, keys_out, perm_out);
+    noalloc_export<<<grid_for(n, 256), 256, 0, s>>>(ni, swapped ? k1 : k0, swapped ? v1 : v0, ss.flag, keys_out, perm_out);
     if (cudaGetLastError() != cudaSuccess) return TG_ERR_CUDA;
     return TG_OK;
 }
