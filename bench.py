@@ -370,7 +370,7 @@ def run_ours(args):
     d2h = 2 * 3 * n * 8
 
     # the plain float64 path against the float32 path on one evaluation of the whole initial state
-    # (same tree and walk; float64 P2P tiles, generic float64 M2L with the potential)
+    # (same tree and walk; float64 P2P and M2L kernels, with the potential)
     fp64 = None
     if rank == 0 and prec == tg.TG_PREC_FP32 and not args.no_fp64_plain:
         fp64 = compare_fp64_plain(tg, rp, run, stream, flush)
@@ -500,8 +500,8 @@ def compare_fp64_plain(tg, rp, run, stream, flush):
     return {"eval_ms_fp64": out["fp64"], "eval_ms_fp32": out["fp32"],
             "value_fp64": n / (out["fp64"] / 1e3), "unit": "particle-forces/s",
             "speedup_of_fp32_path": out["fp64"] / out["fp32"],
-            "note": "one all-from-all evaluation of the initial state: plain float64 path (float64 P2P block per "
-                    "leaf pair, generic float64 M2L, potentials) vs the float32 path (accelerations only)"}
+            "note": "one all-from-all evaluation of the initial state: plain float64 path (float64 P2P and "
+                    "M2L kernels, potentials) vs the float32 path (accelerations only)"}
 
 
 BOX_PARAMS = dict(p=6, theta=0.5, eps=1e-3, kernel=0, n_crit=96, kappa=1.0)
