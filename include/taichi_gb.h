@@ -249,10 +249,19 @@ tg_status tg_get_lists(tg_ctx *ctx, int64_t *m2l_a, int64_t *m2l_b, int64_t *p2p
  *   TG_DEBUG_BATCH_CAPS      value > 0: the next sizing of the batched step starts its list
  *                            capacities at `value` entries and its cell capacity at max(value, 64),
  *                            so that the step overflows, restores the state and regrows.
+ *   TG_DEBUG_SORT_HOLD       value >= 0: tile `value` (2048 particles; not the last one, for which no
+ *                            other waits) of a sort of more than 8192 particles does not publish its
+ *                            counts, and the waits for it are cut short: they run out, and the call
+ *                            returns TG_ERR_TIMEOUT with its outputs or the integrator state as
+ *                            they were.  value < 0 switches it off.
  * TG_ERR_ARG for an unknown `what`.  Not synchronising. */
 typedef enum { TG_DEBUG_FAIL_ALLOC = 1, TG_DEBUG_LIST_CAPACITY = 2, TG_DEBUG_QUEUE_LIMIT = 3,
-               TG_DEBUG_QUEUE_HOLD = 4, TG_DEBUG_BATCH_CAPS = 5 } tg_debug_what;
+               TG_DEBUG_QUEUE_HOLD = 4, TG_DEBUG_BATCH_CAPS = 5, TG_DEBUG_SORT_HOLD = 6 } tg_debug_what;
 tg_status tg_debug_control(tg_ctx *ctx, int what, int64_t value);
+/* tg_morton_sort_noalloc with tile hold_tile held as by TG_DEBUG_SORT_HOLD (< 0: none): every entry of
+ * perm_out is then -1. */
+tg_status tg_debug_morton_sort_noalloc(int64_t n, const double *pos, uint64_t *keys_out, int64_t *perm_out,
+                                       void *cuda_stream, int hold_tile);
 
 /* ---- autotuner (the paper has no counterpart: it picks launch shapes and the leaf size of Sec. 2.3
  * for this GPU and this particle distribution) ----

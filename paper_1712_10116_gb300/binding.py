@@ -128,6 +128,8 @@ def load() -> C.CDLL:
             L.tg_timesteps.argtypes = [_vp, _i64, _vp, _vp, _vp, _vp, _vp]
             L.tg_morton_sort_noalloc.argtypes = [_i64, _vp, _vp, _vp, _vp]
             L.tg_morton_sort_noalloc.restype = C.c_int
+            L.tg_debug_morton_sort_noalloc.argtypes = [_i64, _vp, _vp, _vp, _vp, C.c_int]
+            L.tg_debug_morton_sort_noalloc.restype = C.c_int
             L.tg_debug_control.argtypes = [_vp, C.c_int, _i64]
             L.tg_autotune.argtypes = [_vp, _i64, _vp, _vp, _vp, C.POINTER(tg_tuning)]
             L.tg_ensemble_step.argtypes = [C.POINTER(_vp), C.c_int]
@@ -331,6 +333,7 @@ TG_DEBUG_LIST_CAPACITY = 2
 TG_DEBUG_QUEUE_LIMIT = 3
 TG_DEBUG_QUEUE_HOLD = 4
 TG_DEBUG_BATCH_CAPS = 5
+TG_DEBUG_SORT_HOLD = 6
 
 
 def tg_debug_control(ctx, what: int, value: int):

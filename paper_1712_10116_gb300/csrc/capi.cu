@@ -373,6 +373,11 @@ tg_status tg_debug_control(tg_ctx *c, int what, int64_t value)
         c->debug_batch_caps = value < 0 ? 0 : value;
         if (c->hold) hold_graph_reset_sizes(c);
         return TG_OK;
+    case TG_DEBUG_SORT_HOLD:
+        if (value > INT32_MAX) return set_err(c, TG_ERR_ARG, "tg_debug_control: tile out of range");
+        c->debug_sort_hold = value < 0 ? -1 : (int)value;
+        c->alloc_epoch += 1;   // captured graphs hold the sort's arguments
+        return TG_OK;
     case TG_DEBUG_LIST_CAPACITY:
         if (value <= 0) return set_err(c, TG_ERR_ARG, "tg_debug_control: list capacity estimate must be > 0");
         c->walk_front_per_cell = c->walk_blocks_per_cell = c->walk_p2p_per_cell = (double)value / 1000.0;

@@ -1199,7 +1199,7 @@ __global__ void walk_init_dev(const DevEval *de, uint2 *front, unsigned long lon
         if (de->ncell == 1) {
             p2p[cap_p2p - 1] = make_uint2(0, 0);   // the root is a leaf: one self pair
             ctr[4] = 1ull;
-        } else {
+        } else if (de->ncell > 1) {   // (an evaluation whose sort gave up has no cells)
             front[0] = make_uint2(0, 0);
             ctr[8] = 1ull;
         }

@@ -408,14 +408,17 @@ __global__ void hold_begin(HoldState *h, DevEval *de, LevelLayout lv, int64_t n,
 // One iteration of the loop: advance the frames of Algorithm 1 to the next operation.  Phases of a
 // frame: 0 split; 1 after the split (recurse into level k + 1 with calc = 0 if there is a fast set);
 // 2 first kick pair and drift; 3 second kick pair; 4 the Eq. (9) evaluation at rung 0; 5 recurse with
-// calc = 1; 6 return.  Kick pairs without slow sinks are skipped, as in the host recursion.
-__global__ void hold_sched(HoldState *h, int k_max, int eq9, cudaGraphConditionalHandle h_loop,
+// calc = 1; 6 return.  Kick pairs without slow sinks are skipped, as in the host recursion.  An evaluation whose sort
+// gave up has no accelerations: the loop ends there, and the host restores the state.
+__global__ void hold_sched(HoldState *h, const DevEval *de, int k_max, int eq9, cudaGraphConditionalHandle h_loop,
                            cudaGraphConditionalHandle h_split, cudaGraphConditionalHandle h_eval)
 {
     int op = kOpNone;
     h->iterations += 1ull;
     if (h->iterations > h->limit) {
         h->status = 1;   // bounded: give up, the host restores the state and reports a timeout
+        op = kOpDone;
+    } else if (de->overflow & kSortGaveUp) {
         op = kOpDone;
     } else if (!h->hold) {
         for (int guard = 0; guard < 8 * kHoldLevels && op == kOpNone; ++guard) {
@@ -834,7 +837,7 @@ static tg_status hold_capture_into(tg_ctx *c, HoldGraph *g, Sched &s, const std:
         return r;
     };
     if ((st = capture_begin(c, g, body))) return restore(st);
-    hold_sched<<<1, 1, 0, c->stream>>>(h, c->prm.k_max, eq9, h_loop, h_split, h_eval);
+    hold_sched<<<1, 1, 0, c->stream>>>(h, de, c->prm.k_max, eq9, h_loop, h_split, h_eval);
     if ((st = capture_end(c, g))) return restore(st);
     cudaGraphNode_t sched_node;
     size_t nn = 1;
@@ -996,7 +999,7 @@ tg_status hhs_step_batched(tg_ctx *c)
         if (head.status != 0)
             return fail(set_err(c, TG_ERR_TIMEOUT, "batched step: the device loop stopped after %llu iterations",
                                 head.iterations));
-        if (overflow & 8u) return fail(set_err(c, TG_ERR_TIMEOUT, "batched step: a bounded wait of the particle sort ran out"));
+        if (overflow & kSortGaveUp) return fail(set_err(c, TG_ERR_TIMEOUT, "batched step: a bounded wait of the particle sort ran out"));
         if (overflow) {
             // restore, grow what ran out, capture again and redo the step
             restore_state(c, s, static_cast<const char *>(c->buf[B_SNAP].p));
@@ -1144,7 +1147,7 @@ tg_status ensemble_step(tg_ctx **cs, int count)
                                                             "iterations", i, head.iterations);
             continue;
         }
-        if (overflow & 8u) {
+        if (overflow & kSortGaveUp) {
             restore_state(c, sched[i], static_cast<const char *>(c->buf[B_SNAP].p));
             if (!first) first = set_err(c0, TG_ERR_TIMEOUT, "ensemble member %d: a bounded wait of the particle sort ran out", i);
             continue;

@@ -175,6 +175,7 @@ tg_status launch_m2l_f32(tg_ctx *c, const TreeView &t, const M2LBlock *blocks, i
 __global__ void m2l_list_check(const uint32_t *off, const uint32_t *cnt, DevEval *de, uint64_t cap)
 {
     const int last = de->ncell - 1;
+    if (last < 0) return;
     if ((uint64_t)off[last] + cnt[last] > cap) de->overflow |= 4u;
 }
 

@@ -78,8 +78,7 @@ int check_dev(const void *p)
 
 }  // namespace
 
-extern "C" tg_status tg_morton_sort_noalloc(int64_t n, const double *pos, uint64_t *keys_out, int64_t *perm_out,
-                                            void *cuda_stream)
+static tg_status morton_sort(int64_t n, const double *pos, uint64_t *keys_out, int64_t *perm_out, void *cuda_stream, int hold)
 {
     if (n < 0 || n > kMaxN) return TG_ERR_ARG;
     if (n == 0) return TG_OK;
@@ -100,9 +99,21 @@ extern "C" tg_status tg_morton_sort_noalloc(int64_t n, const double *pos, uint64
     int launches;
     const SortScratch ss = sort_scratch(base + kOffSort, n);
     if (launch_sort(s, ni, nullptr, pos, n, nullptr, nullptr, nullptr, geom, k0, k1, v0, v1, ss, SortedOut{},
-                    &swapped, &gathered, &launches) != cudaSuccess)
+                    hold, &swapped, &gathered, &launches) != cudaSuccess)
         return TG_ERR_CUDA;
     noalloc_export<<<grid_for(n, 256), 256, 0, s>>>(ni, swapped ? k1 : k0, swapped ? v1 : v0, ss.flag, keys_out, perm_out);
     if (cudaGetLastError() != cudaSuccess) return TG_ERR_CUDA;
     return TG_OK;
+}
+
+extern "C" tg_status tg_morton_sort_noalloc(int64_t n, const double *pos, uint64_t *keys_out, int64_t *perm_out,
+                                            void *cuda_stream)
+{
+    return morton_sort(n, pos, keys_out, perm_out, cuda_stream, -1);
+}
+
+extern "C" tg_status tg_debug_morton_sort_noalloc(int64_t n, const double *pos, uint64_t *keys_out, int64_t *perm_out,
+                                                  void *cuda_stream, int hold_tile)
+{
+    return morton_sort(n, pos, keys_out, perm_out, cuda_stream, hold_tile < 0 ? -1 : hold_tile);
 }

@@ -98,7 +98,9 @@ __global__ void __launch_bounds__(kOctThreads) oct_levels(const uint64_t *__rest
 
 // Exclusive scan of cnt (levels 0 .. max_level, ntile entries each), and the sizes of the tree.  One block: the
 // array holds (max_level + 1) entries per 1024 particles.  Levels beyond `levels` or cells beyond `cap` (batched
-// path) are cut off: the tree then ends at the last level that fits, and the step is redone.
+// path) are cut off: the tree then ends at the last level that fits, and the step is redone.  After a sort that gave
+// up the keys are in no order: the evaluation then goes on without cells and without particles, so that nothing behind it
+// reads a cell or an index.
 __global__ void __launch_bounds__(1024) oct_scan(int n, const int *dn, int max_level, uint32_t *cnt, DevEval *de, int cap,
                                                  int levels, const uint32_t *flag)
 {
@@ -149,7 +151,9 @@ __global__ void __launch_bounds__(1024) oct_scan(int n, const int *dn, int max_l
     uint32_t over = 0u;
     int nlev = 0;
     de->level_begin[0] = 0;
-    for (int l = 0; l <= max_level; ++l) {
+    const bool unsorted = ((flag ? *flag : de->overflow) & kSortGaveUp) != 0;
+    if (unsorted) de->n = 0;
+    for (int l = 0; l <= max_level && !unsorted; ++l) {
         const int begin = (int)cnt[(size_t)l * ntile], end = l < max_level ? (int)cnt[(size_t)(l + 1) * ntile] : total;
         if (end == begin) break;
         if (end > cap) {
@@ -305,7 +309,7 @@ tg_status build_octree(tg_ctx *c, int n, int *ncell_out)
     cudaError_t e = stream_sync(c);
     if (e != cudaSuccess) return cuda_check(c, e, "octree");
     c->walk_log2L = *reinterpret_cast<int *>(c->h_pinned + 32);
-    if (h->overflow & 8u) {
+    if (h->overflow & kSortGaveUp) {
         cudaMemsetAsync(c->buf[B_SORT].p, 0, 256, c->stream);
         return set_err(c, TG_ERR_TIMEOUT, "a bounded wait of the particle sort ran out");
     }

@@ -134,6 +134,7 @@ struct tg_ctx {
     unsigned debug_queue_limit = 0;  // tg_debug_control: iteration limit of the device loop (0: default)
     int debug_queue_hold = 0;        // tg_debug_control: the scheduler publishes no operation
     int64_t debug_batch_caps = 0;    // tg_debug_control: initial capacities of the batched step
+    int debug_sort_hold = -1;        // tg_debug_control: this tile of the particle sort publishes nothing
 };
 
 namespace tg {
@@ -278,8 +279,9 @@ constexpr int kSortPasses = (63 + kSortBits - 1) / kSortBits;
 constexpr int kSmallSort = 8192;         // up to here one block sorts in shared memory
 constexpr int kBoxThreads = 256, kBoxBlocks = 2 * 152;
 constexpr int kScanThreads = 512;        // threads per scan block
+constexpr uint32_t kSortGaveUp = 8u;     // a bounded wait of the sort ran out (SortScratch::flag, DevEval::overflow bit 3)
 struct SortScratch {
-    uint32_t *done, *flag;   // blocks of root_cube that finished; 8 when a bounded wait ran out
+    uint32_t *done, *flag;   // blocks of root_cube that finished; kSortGaveUp once a bounded wait ran out
     double *boxes;           // a bounding box per block of root_cube
     uint32_t *state[2];      // digit counts and sums of the tiles, by pass parity
     uint32_t *hist;          // digit counts of the seven passes, then their tickets
@@ -293,7 +295,7 @@ SortScratch sort_scratch(void *base, int64_t n);
 tg_status ensure_sort_scratch(tg_ctx *c, int64_t n, void **out);
 cudaError_t launch_sort(cudaStream_t st, int n, const int *dn, const double *pos, int64_t stride, const int64_t *sub,
                         const double *mass, const uint8_t *fast, Geom *g, uint64_t *k0, uint64_t *k1, uint32_t *v0,
-                        uint32_t *v1, const SortScratch &s, const SortedOut &o, bool *swapped, bool *gathered, int *launches);
+                        uint32_t *v1, const SortScratch &s, const SortedOut &o, int hold, bool *swapped, bool *gathered, int *launches);
 
 // ---- fmm.cu
 // Full FMM evaluation on a (sub)set of particles.  Outputs are in input order q:

@@ -441,7 +441,9 @@ __global__ void __launch_bounds__(256) morton_keys(const double *pos, int64_t st
 // this and all earlier tiles, (sum << 2) | 2, once it is; a tile adds up its predecessors' words backwards until
 // it meets a sum (decoupled look-back, Merrill and Garland 2016).  Tiles are handed out by a ticket, so a tile
 // only waits for blocks that already run and wait for nothing before they publish; the wait is bounded all the
-// same and raises s.flag when it runs out.  Each pass clears the other pass's states.
+// same and raises s.flag when it runs out.  A pass that gave up leaves part of its output unwritten, so nothing
+// reads the sorted indices while the flag is up: the gather returns, the octree comes out empty, and the host
+// reports TG_ERR_TIMEOUT.  Each pass clears the other pass's states.
 // Bound by latency up to a million items (10 us a pass at 54,321, where a histogram launch, one to three scan
 // launches and a scatter launch took 28; the whole allocation-free sort of 200,001 went from 231 to 116 us) and at
 // 1.7 TB/s beyond (4,194,304 items: 61 us a pass, about 85 before).  Reading 4 / 8 / 16 predecessors at a time: 123 / 116 /
@@ -449,12 +451,14 @@ __global__ void __launch_bounds__(256) morton_keys(const double *pos, int64_t st
 constexpr int kSortThreads = 256;
 constexpr int kSortItems = 8;
 constexpr unsigned kSortSpin = 1u << 18;   // some 0.2 s; a wait lasts microseconds
+constexpr unsigned kSortSpinHeld = 1u << 10;   // with a held tile, which every wait runs into
 static_assert(kSortBins == 2 * kSortThreads, "two digits to each thread");
 static_assert(kSortThreads * kSortItems == kSortTileItems, "tile size");
 
 // Sums over the tiles before `tile` of a thread's two digit counts (one 64-bit word per tile and thread, so both
 // flags change at once).  Eight predecessors are read at a time: their loads overlap.
 constexpr int kSortAhead = 8;
+template <unsigned LIMIT>
 __device__ __forceinline__ uint2 look_back(const volatile unsigned long long *state, int tile, uint32_t *flag)
 {
     uint2 sum = make_uint2(0u, 0u);
@@ -473,18 +477,21 @@ __device__ __forceinline__ uint2 look_back(const volatile unsigned long long *st
             if (lo & 2u) return sum;   // tile 0 always holds a sum
             spins = 0;
         }
-        if (++spins > kSortSpin) {
-            atomicOr(flag, 8u);
+        if (++spins > LIMIT) {
+            atomicOr(flag, kSortGaveUp);
             return sum;
         }
     }
     return sum;
 }
 
+// HELD: the test hook, a variant of its own (the tile and the limit as arguments of the one kernel made a sort of
+// 200,001 particles 123 us instead of 116).
+template <bool HELD>
 __global__ void __launch_bounds__(kSortThreads) radix_pass(const uint64_t *__restrict__ keys_in,
                                                            const uint32_t *__restrict__ vals_in, uint64_t *keys_out,
                                                            uint32_t *vals_out, int n, const int *dn, int pass,
-                                                           SortScratch s)
+                                                           SortScratch s, int hold)
 {
     n = dev_or(dn, n);
     if (dn && n <= kSmallSort) return;
@@ -546,7 +553,7 @@ __global__ void __launch_bounds__(kSortThreads) radix_pass(const uint64_t *__res
         reinterpret_cast<volatile unsigned long long *>(state) + (size_t)tile * kSortThreads + threadIdx.x;
     {
         const uint32_t f = tile == 0 ? 2u : 1u;
-        *mine = (unsigned long long)((tot[0] << 2) | f) | ((unsigned long long)((tot[1] << 2) | f) << 32);
+        if (!HELD || tile != hold) *mine = (unsigned long long)((tot[0] << 2) | f) | ((unsigned long long)((tot[1] << 2) | f) << 32);
         reinterpret_cast<uint2 *>(s.state[(pass + 1) & 1] + (size_t)tile * kSortBins)[threadIdx.x] = make_uint2(0u, 0u);
     }
     // exclusive scans over the digits: of the tile's totals (with the padding, which sits at the end) and of the
@@ -584,8 +591,10 @@ __global__ void __launch_bounds__(kSortThreads) radix_pass(const uint64_t *__res
     // where the tile's run of each digit goes, less its place in the tile
     uint2 pre = make_uint2(0u, 0u);
     if (tile > 0) {
-        pre = look_back(reinterpret_cast<const volatile unsigned long long *>(state) + threadIdx.x, tile, s.flag);
-        *mine = (unsigned long long)(((pre.x + tot[0]) << 2) | 2u) | ((unsigned long long)(((pre.y + tot[1]) << 2) | 2u) << 32);
+        pre = look_back<HELD ? kSortSpinHeld : kSortSpin>(
+            reinterpret_cast<const volatile unsigned long long *>(state) + threadIdx.x, tile, s.flag);
+        if (!HELD || tile != hold)
+            *mine = (unsigned long long)(((pre.x + tot[0]) << 2) | 2u) | ((unsigned long long)(((pre.y + tot[1]) << 2) | 2u) << 32);
     }
     place[2 * threadIdx.x] = hexcl + pre.x - excl;
     place[2 * threadIdx.x + 1] = hexcl + all.x + pre.y - (excl + tot[0]);
@@ -612,10 +621,12 @@ __device__ __forceinline__ void gather_one(int64_t s, uint32_t q, const double *
 }
 
 __global__ void gather_sorted(const uint32_t *perm, const double *pos, int64_t stride, const int64_t *sub,
-                              const double *mass, const uint8_t *fast, int n, const int *dn, SortedOut o)
+                              const double *mass, const uint8_t *fast, int n, const int *dn, const uint32_t *flag,
+                              SortedOut o)
 {
     n = dev_or(dn, n);
     if (dn && n <= kSmallSort) return;
+    if (*flag & kSortGaveUp) return;   // perm is incomplete: indices of an earlier call or none at all
     for (int64_t s = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; s < n; s += (int64_t)gridDim.x * blockDim.x)
         gather_one(s, perm[s], pos, stride, sub, mass, fast, o);
 }
@@ -764,10 +775,10 @@ SortScratch sort_scratch(void *base, int64_t n)
 
 // Root cube, keys and sort on a stream: the sorted keys and indices end in k0 / v0 when *swapped is false, in k1 / v1
 // when it is true.  With o the small sort also gathers (*gathered).  dn: device count (n is then the capacity,
-// and the launches of both sizes are issued).
+// and the launches of both sizes are issued).  hold: test hook, the tile that publishes nothing (< 0: none).
 cudaError_t launch_sort(cudaStream_t st, int n, const int *dn, const double *pos, int64_t stride, const int64_t *sub,
                         const double *mass, const uint8_t *fast, Geom *g, uint64_t *k0, uint64_t *k1, uint32_t *v0,
-                        uint32_t *v1, const SortScratch &s, const SortedOut &o, bool *swapped, bool *gathered, int *launches)
+                        uint32_t *v1, const SortScratch &s, const SortedOut &o, int hold, bool *swapped, bool *gathered, int *launches)
 {
     static_assert(kSortPasses % 2 == 1, "an odd number of passes ends in the second pair of buffers");
     *swapped = *gathered = false;
@@ -789,7 +800,8 @@ cudaError_t launch_sort(cudaStream_t st, int n, const int *dn, const double *pos
     morton_keys<<<grid_for(n, 256, 152 * 8), 256, 0, st>>>(pos, stride, sub, n, dn, g, k0, v0, s);
     for (int pass = 0; pass < kSortPasses; ++pass) {
         const bool odd = pass & 1;
-        radix_pass<<<nt, kSortThreads, 0, st>>>(odd ? k1 : k0, odd ? v1 : v0, odd ? k0 : k1, odd ? v0 : v1, n, dn, pass, s);
+        (hold < 0 ? radix_pass<false> : radix_pass<true>)<<<nt, kSortThreads, 0, st>>>(
+            odd ? k1 : k0, odd ? v1 : v0, odd ? k0 : k1, odd ? v0 : v1, n, dn, pass, s, hold);
     }
     *swapped = true;
     *launches += 2 + kSortPasses;
@@ -819,8 +831,8 @@ tg_status sort_particles(tg_ctx *c, int n, const double *pos, int64_t stride, co
     if (de) s.flag = const_cast<uint32_t *>(&de->overflow);
     {
         ProfScope ps_(c, TG_K_TREE);
-        e = launch_sort(c->stream, n, dn, pos, stride, sub, mass, fast, d_geom, k0, k1, v0, v1, s, o, &swapped, &gathered,
-                        &launches);
+        e = launch_sort(c->stream, n, dn, pos, stride, sub, mass, fast, d_geom, k0, k1, v0, v1, s, o,
+                        c->debug_sort_hold, &swapped, &gathered, &launches);
         c->prof_launches[TG_K_TREE] += launches - 1;
     }
     if (e != cudaSuccess) return cuda_check(c, e, "keys and sort");
@@ -831,7 +843,8 @@ tg_status sort_particles(tg_ctx *c, int n, const double *pos, int64_t stride, co
     }
     if (!gathered) {
         ProfScope ps_(c, TG_K_TREE);
-        gather_sorted<<<grid_for(n, 256), 256, 0, c->stream>>>(swapped ? v1 : v0, pos, stride, sub, mass, fast, n, dn, o);
+        gather_sorted<<<grid_for(n, 256), 256, 0, c->stream>>>(swapped ? v1 : v0, pos, stride, sub, mass, fast, n, dn,
+                                                               s.flag, o);
     }
     return cuda_check(c, cudaGetLastError(), "keys/sort/gather");
 }
