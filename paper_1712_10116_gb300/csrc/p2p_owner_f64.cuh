@@ -49,7 +49,9 @@ struct Own64Shared {
 };
 
 // Rows i0 .. i0 + 32*ROWS of one phase (0: slow rows, 1: fast rows) against the first ncol staged columns
-// (a multiple of 4); the reaction sums of columns at or past nkeep are not kept.  Lane l visits column
+// (a multiple of 4).  Columns at or past nkeep are massless and their reaction sums are not kept; pairs with
+// one, or with a slot that holds no row, are evaluated at r = 1, where the value is finite whatever the softening and
+// the coordinates are (the two selects run on the integer pipe).  Lane l visits column
 // c ^ ((l >> 3) & 3) of a batch at step c, so that the column stages of the reduce-scatter (partners l^16,
 // l^8) need no selects.
 //
@@ -70,8 +72,7 @@ __device__ __noinline__ void owner_rows_f64(const Bodies &pf, const Own64Batch *
     for (int r = 0; r < ROWS; ++r) {
         const int i = i0 + (lane & (32 / S - 1)) + 32 * r;
         gi[r] = -1;
-        p[r].x = p[r].y = p[r].z = 1e8;   // far away, massless
-        p[r].w = 0.0;
+        p[r].x = p[r].y = p[r].z = p[r].w = 0.0;   // massless
         if (i < nrows) {
             int s = 0;   // slot: the first with inc[s] > i
 #pragma unroll
@@ -89,13 +90,15 @@ __device__ __noinline__ void owner_rows_f64(const Bodies &pf, const Own64Batch *
 #pragma unroll
         for (int c = 0; c < 4 / S; ++c) {
             const dbl4 q = sq[j0 + (c ^ cperm)];
+            const bool column = j0 + (c ^ cperm) < nkeep;
 #pragma unroll
             for (int e = 0; e < NC; ++e) col[c][e] = 0.0;
 #pragma unroll
             for (int r = 0; r < ROWS; ++r) {
                 const double dx = q.x - p[r].x, dy = q.y - p[r].y, dz = q.z - p[r].z;
                 double g, ri;
-                pair_f64<KERNEL, POT>(pair_s2<KERNEL>(dx, dy, dz, k), k, g, ri);
+                const double s = pair_s2<KERNEL>(dx, dy, dz, k);
+                pair_f64<KERNEL, POT>(column && gi[r] >= 0 ? s : 1.0, k, g, ri);
                 const double mq = q.w * g, mp = p[r].w * g;
                 ra[r][0] = fma(mq, dx, ra[r][0]);
                 ra[r][1] = fma(mq, dy, ra[r][1]);
@@ -190,16 +193,17 @@ __device__ __noinline__ void self_pair_f64(const Bodies &pf, int fa, int na, int
             const bool row = i < na, slow = i < sa;
             const int jend = i0 < sa ? nbc : min(nbc, sa - jc);   // fast rows stop at the slow columns
             dbl4 p;
-            p.x = p.y = p.z = 1e8;
-            p.w = 0.0;
+            p.x = p.y = p.z = p.w = 0.0;
             if (row) p = pf.get(fa + i);
             double ax = 0, ay = 0, az = 0, ph = 0;
             for (int j = slice; j < jend; j += 4) {
                 const dbl4 q = sq[j];
-                const double m = (jc + j != i && (slow || jc + j < sa)) ? q.w : 0.0;
+                const bool use = jc + j != i && (slow || jc + j < sa);
+                const double m = use ? q.w : 0.0;
                 const double dx = q.x - p.x, dy = q.y - p.y, dz = q.z - p.z;
                 double g, ri;
-                pair_f64<KERNEL, POT>(pair_s2<KERNEL>(dx, dy, dz, k), k, g, ri);
+                const double s = pair_s2<KERNEL>(dx, dy, dz, k);
+                pair_f64<KERNEL, POT>(use ? s : 1.0, k, g, ri);   // excluded: r = 1, finite at any softening
                 const double mg = m * g;
                 ax = fma(mg, dx, ax);
                 ay = fma(mg, dy, ay);
@@ -285,7 +289,7 @@ __global__ void __launch_bounds__(32 * kOwn64Warps)
         const int Ts = __shfl_sync(0xffffffffu, incS, 31), Tf = __shfl_sync(0xffffffffu, incF, 31);
         if (Ts == 0 && (Tf == 0 || sB == 0)) continue;   // nothing but fast-fast pairs
         for (int jc = 0; jc < nb; jc += kMaxNcrit) {
-            // columns in leaf order (slow first), padded to a multiple of 4 with massless far particles; without
+            // columns in leaf order (slow first), padded to a multiple of 4 with massless ones; without
             // slow rows only the slow columns are staged
             const int nbc = min(kMaxNcrit, nb - jc), nsc = max(0, min(sB - jc, nbc));
             const int ns4 = (nsc + 3) & ~3, nt4 = (nbc + 3) & ~3;
@@ -294,14 +298,13 @@ __global__ void __launch_bounds__(32 * kOwn64Warps)
             __syncwarp();
             for (int j = lane; j < nstage; j += 32) {
                 dbl4 q;
-                q.x = q.y = q.z = -1e8;
-                q.w = 0.0;
+                q.x = q.y = q.z = q.w = 0.0;
                 if (j < nbc) q = pf.get(fb + jc + j);
                 sq[j] = q;
                 sacc[j][0] = sacc[j][1] = sacc[j][2] = sacc[j][3] = 0.0;
             }
             __syncwarp();
-            owner_phase_f64<KERNEL, POT>(pf, ob, 0, Ts, sq, sacc, nt4, nt4, k, acc4, n, lane);
+            owner_phase_f64<KERNEL, POT>(pf, ob, 0, Ts, sq, sacc, nt4, nbc, k, acc4, n, lane);
             if (nsc > 0 && Tf > 0) {
                 // fast rows meet the slow columns only: the fast columns of the last batch are made massless and
                 // their reaction sums dropped
