@@ -358,11 +358,16 @@ __device__ __forceinline__ int warp_incl_scan(int v, int lane)
 // counters on the device (they sit at the end of the P2P buffer of capacity cap_p2p).
 //
 // Bound by the latency of dependent packed operations: three blocks of 256 per SM (80 registers a thread, part of the
-// units' bookkeeping spilled) beat two (128 registers) although they spill.  Two rows per lane: disk galaxy 15.9
-// against 17.1 ms, 2^20 sphere 5.45 against 5.67; one row 18.3 against 19.7 and 6.50 against 6.77.  Three rows keep
-// two blocks (17.1 and 5.38; three blocks: 18.4 and 5.46).
+// units' bookkeeping spilled) beat two (128 registers) as long as little enough is spilled.  Without the potential, two
+// rows per lane: kick pair of the disk galaxy 15.9 ms with three against 17.1 with two, 2^20 sphere 5.45 / 5.66,
+// 2^20 Plummer sphere 3.89 / 4.16; Plummer softening on the same three 23.3 / 24.3 (whole disk), 7.52 / 7.67,
+// 5.07 / 5.29.  One row: 18.3 / 19.7 and 6.50 / 6.77, with the potential 23.0 / 24.6 (disk), 7.34 / 7.64, 5.05 / 5.38.
+// Two rows with the potential spill twice as much: 21.57 / 21.05 (disk), 6.54 / 6.45, 5.11 / 4.70, and level with
+// Plummer softening (26.3 / 26.5, 8.47 / 8.37, 5.74 / 5.76): two blocks.  Three rows: two blocks (without the potential
+// 17.1 and 5.38; three blocks 18.4 and 5.46).
+__host__ __device__ constexpr int owner_blocks(int rows, bool pot) { return rows == 1 || (rows == 2 && !pot) ? 3 : 2; }
 template <int KERNEL, int ROWS, bool POT>
-__global__ void __launch_bounds__(256, ROWS == 3 ? 2 : 3) p2p_owner_f32(TreeView t, int log2L, const uint2 *__restrict__ units,
+__global__ void __launch_bounds__(256, owner_blocks(ROWS, POT)) p2p_owner_f32(TreeView t, int log2L, const uint2 *__restrict__ units,
                                                         uint32_t *ctr, const uint32_t *__restrict__ own_off,
                                                         const uint32_t *__restrict__ own_cnt,
                                                         const int32_t *__restrict__ partners, int64_t npairs,
@@ -509,23 +514,8 @@ __global__ void __launch_bounds__(256, ROWS == 3 ? 2 : 3) p2p_owner_f32(TreeView
 
 namespace tg {
 
-// Resident blocks per SM of the owner kernel, queried once per rows-per-lane setting (tg_autotune: 1,
-// 2 or 3; rows are packed densely, so the chunk is full whatever the leaf size).
-static int owner_occupancy(int rows)
-{
-    static int occ[4] = {0, 0, 0, 0};
-    if (occ[rows] == 0) {
-        cudaError_t e = cudaErrorInvalidValue;
-        if (rows == 1) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ[1], p2p_owner_f32<TG_KERNEL_WENDLAND_C2, 1, false>, 256, 0);
-        if (rows == 2) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ[2], p2p_owner_f32<TG_KERNEL_WENDLAND_C2, 2, false>, 256, 0);
-        if (rows == 3) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ[3], p2p_owner_f32<TG_KERNEL_WENDLAND_C2, 3, false>, 256, 0);
-        if (e != cudaSuccess || occ[rows] < 1) {
-            cudaGetLastError();
-            occ[rows] = 1;
-        }
-    }
-    return occ[rows];
-}
+// Resident blocks per SM of the owner kernel (tg_autotune: 1, 2 or 3 rows per lane; rows are packed densely, so the
+// chunk is full whatever the leaf size): the launch bound's, which registers and shared memory allow.
 
 // The distinct leaf pairs grouped by owner (both precisions).
 struct OwnerLists {
@@ -612,7 +602,7 @@ tg_status launch_p2p_f32(tg_ctx *c, const TreeView &t, const uint2 *pairs, int64
     const bool plummer = c->prm.kernel == TG_KERNEL_PLUMMER;
     ProfScope ps_(c, TG_K_P2P);
     const int rows = c->tune.p2p_rows;
-    const int grid = c->num_sms * owner_occupancy(rows);
+    const int grid = c->num_sms * owner_blocks(rows, pot);
 #define TG_OWNER(K, R, PT)                                                                                        \
     p2p_owner_f32<K, R, PT><<<grid, 256, 0, c->stream>>>(t, c->walk_log2L, o.units, o.ctr, o.off, o.cnt, o.partners, \
                                                          npairs, self_pairs, (uint32_t)nself, pf, nslow, eps, acc4, t.n, pc,    \
@@ -649,7 +639,7 @@ tg_status launch_p2p_f32_dev(tg_ctx *c, const TreeView &t, const DevEval *de, co
     const bool plummer = c->prm.kernel == TG_KERNEL_PLUMMER;
     ProfScope ps_(c, TG_K_P2P);
     const int rows = c->tune.p2p_rows;
-    const int grid = c->num_sms * owner_occupancy(rows);
+    const int grid = c->num_sms * owner_blocks(rows, false);
 #define TG_OWNER_DEV(K, R)                                                                                        \
     p2p_owner_f32<K, R, false><<<grid, 256, 0, c->stream>>>(t, 0, o.units, o.ctr, o.off, o.cnt, o.partners, 0, nullptr, 0u, \
                                                             pf, nslow, eps, acc4, stride, pc, gp, walk_ctr, p2p,    \
