@@ -689,7 +689,7 @@ static tg_status hold_presize(tg_ctx *c, const Sched &s, const BatchCaps &cap, c
     const int n = cap.n, C = cap.cells, p_ = c->prm.p, ncp = (ncoef(p_) + 3) & ~3;
     const size_t rows = (size_t)C * 2;
     const int nh = (p_ + 1) * (p_ + 1), ncpr = (nh + 3) & ~3;
-    const int64_t max_units = (int64_t)cap.p2p / 8 + std::min<int64_t>((int64_t)cap.p2p, 32768) + C + 1;   // own_max_units
+    const int64_t max_units = own_max_units((int64_t)cap.p2p, C);
     const size_t tsz = c->prm.precision == TG_PREC_FP32 ? 4 : 8;   // compute precision
     struct Need { int slot; size_t bytes; };
     const Need needs[] = {

@@ -19,8 +19,6 @@
 // than eps to the owner's come first; chunks made only of the other partners' rows need no softening
 // test, the others take the pair value at max(r, eps) and correct the rare pairs with r < eps.
 #pragma once
-#include <algorithm>
-
 #include "p2p_tile.cuh"
 
 namespace tg {
@@ -39,8 +37,6 @@ __host__ __device__ __forceinline__ int own_unit(int64_t npairs, bool f64)
     while (u < 32 && ((int64_t)u << 14) < npairs) u <<= 1;
     return u;
 }
-// capacity of the unit list: every owner opens one unit more than its full ones
-inline int64_t own_max_units(int64_t npairs, int64_t ncell) { return npairs / 8 + std::min<int64_t>(npairs, 32768) + ncell + 1; }
 
 // Owner and partner of each distinct leaf pair, and per-owner partner counts (own_cnt starts at zero).
 // The walk writes the pairs of one row cell side by side, so lanes of a warp often share an owner:

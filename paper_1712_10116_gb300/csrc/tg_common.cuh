@@ -259,6 +259,9 @@ tg_status launch_m2l_f64_dev(tg_ctx *c, const TreeView &t, const DevEval *de, co
 tg_status launch_m2l_f64(tg_ctx *c, const TreeView &t, const M2LBlock *blocks, int64_t nblocks, const double *Ms,
                          double *L, int p, int nc, int ncp, bool masked, bool pot, const int32_t *nslow);
 // ---- p2p.cu: mutual P2P of all leaf pairs (distinct pairs and self pairs) into acc4.
+// Capacity of the list of work units (own_unit, p2p_owner.cuh): every owner opens one more than its full ones; units of
+// 8 and more are at most npairs / 8, smaller ones (float64) are at most 32768.
+inline int64_t own_max_units(int64_t npairs, int64_t ncell) { return npairs / 8 + std::min<int64_t>(npairs, 32768) + ncell + 1; }
 tg_status launch_p2p_f32(tg_ctx *c, const TreeView &t, const uint2 *pairs, int64_t npairs, const uint2 *self_pairs,
                          int64_t nself, const float4 *pf, const int32_t *nslow, bool pot, double *acc4);
 tg_status launch_p2p_f32_dev(tg_ctx *c, const TreeView &t, const DevEval *de, const Geom *gp,
