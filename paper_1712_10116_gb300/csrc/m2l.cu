@@ -9,10 +9,10 @@
 
 namespace tg {
 
-// zero n (+ extra) words, n from the device when dn is given (dn[0] + extra)
-__global__ void zero_u32(uint32_t *p, int n, const int *dn, int extra)
+// zero n words, n from the device when dn is given
+__global__ void zero_u32(uint32_t *p, int n, const int *dn)
 {
-    if (dn) n = dn[0] + extra;
+    n = dev_or(dn, n);
     for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) p[i] = 0u;
 }
 
@@ -45,8 +45,8 @@ static tg_status m2l_lists(tg_ctx *c, const TreeView &t, const M2LBlock *blocks,
     const int g = c->num_sms * 8;
     {
         ProfScope ps_(c, TG_K_M2L);
-        zero_u32<<<g, 256, 0, c->stream>>>(cnt, ncell, dncell, 0);
-        zero_u32<<<g, 256, 0, c->stream>>>(fill, ncell, dncell, 0);
+        zero_u32<<<g, 256, 0, c->stream>>>(cnt, ncell, dncell);
+        zero_u32<<<g, 256, 0, c->stream>>>(fill, ncell, dncell);
         m2l_list_count<<<g, 256, 0, c->stream>>>(t, blocks, nblocks, cnt, dnb);
     }
     if ((st = exclusive_scan_u32(c, cnt, off, ncell, nullptr, dncell))) return st;

@@ -349,7 +349,7 @@ __device__ __forceinline__ int warp_incl_scan(int v, int lane)
 // One warp per work unit (own_unit partners of one owner), units taken from a shared counter
 // (ctr[1], starts at zero) so that the load stays balanced whatever the spread of leaf work.  After
 // the units, the same counter hands out the self pairs (A, A): slow rows of A against every particle
-// of A with a larger index, i.e. each slow-slow and slow-fast pair once (p2p_pair_f32, SELF).
+// of A with a larger index, i.e. each slow-slow and slow-fast pair once (p2p_self_f32).
 // Batched path (walk_ctr non-null): the root cube comes from gp and the self pairs from the walk's
 // counters on the device (they sit at the end of the P2P buffer of capacity cap_p2p).
 //
@@ -398,7 +398,7 @@ __global__ void __launch_bounds__(256, owner_blocks(ROWS, POT)) p2p_owner_f32(Tr
             const int fa = t.first[A], na = t.count[A], sa = nslow ? nslow[A] : na;
             if (sa == 0) continue;   // no slow row: every pair of the leaf is fast-fast
             __syncwarp();
-            p2p_pair_f32<KERNEL, true, ROWS, true>(pf, fa, sa, fa, na, 0.f, 0.f, 0.f, eps, acc4, n, lane, sq);
+            p2p_self_f32<KERNEL, ROWS>(pf, fa, sa, na, eps, acc4, n, lane, sq);
             if (lane == 0) {
                 const unsigned long long nf = na - sa;
                 my_pairs += (unsigned long long)na * (na - 1) / 2 - nf * (nf - (nf > 0 ? 1 : 0)) / 2;

@@ -1,21 +1,15 @@
-// p2p_tile.cuh -- mutual particle-particle interaction of leaf pairs (P2P, Sec. 2.1, Eq. 2).
-// Each unordered leaf pair (A, B) is visited once; for every particle pair the kernel value is
-// computed once and applied with opposite signs to both particles (a_i += m_j g d, a_j -= m_i g d).
-// Positions are relative to leaf centres (exact float offsets between centres).  F-F pairs are
-// skipped when classes are given (kickS2F feels slow masses only).
+// p2p_tile.cuh -- float32 P2P of the self pair (A, A) of a leaf (Sec. 2.1, Eq. 2; the distinct leaf pairs are
+// p2p_owner.cuh's).  For every particle pair the kernel value is computed once and applied with opposite signs to both
+// particles (a_i += m_j g d, a_j -= m_i g d).  Positions are relative to the leaf's centre.  F-F pairs are skipped when
+// classes are given (kickS2F feels slow masses only): the rows are the slow particles, which come first.
 #pragma once
 #include "p2p_pair.cuh"
 #include "tg_common.cuh"
 
 namespace tg {
 
-// ------------------------------------------------------------------ float32 warp tiles
-// Building blocks of the float32 P2P launch (p2p_owner.cuh): the pair value and the tile of one
-// leaf pair, used there for the self pairs (A, A).
-
 // float32 pair value: Newton by default, Wendland correction inside eps (rare, predicated).
-// NEAR = false: the caller knows r >= eps for every pair (leaf cubes at least eps apart).
-template <int KERNEL, bool NEAR = true>
+template <int KERNEL>
 __device__ __forceinline__ void pair_kernel_f32(float r2, float eps, float eps2, float inv_eps, float inv_eps3, float &g,
                                                 float &phi)
 {
@@ -25,44 +19,38 @@ __device__ __forceinline__ void pair_kernel_f32(float r2, float eps, float eps2,
         g = si * si * si;
         return;
     }
-    const float ri = NEAR ? rsqrtf(r2) : rsqrt_ftz(r2);   // far pairs: r2 >= eps^2
+    const float ri = rsqrtf(r2);
     phi = -ri;
     g = ri * ri * ri;
-    if (NEAR && r2 < eps2) pair_kernel<float, TG_KERNEL_WENDLAND_C2>(r2, eps, eps2, inv_eps, inv_eps3, g, phi);
+    if (r2 < eps2) pair_kernel<float, TG_KERNEL_WENDLAND_C2>(r2, eps, eps2, inv_eps, inv_eps3, g, phi);
 }
 
-// One leaf pair.  Rows = particles of A, ROWS per lane (row i0 + lane + 32 r), chunks of 32*ROWS;
-// columns = particles of B, staged once in the warp's shared-memory slice (positions shifted into
-// A's frame) and read in batches of 8.  A lane keeps its rows' sums in registers and its 8 x 4
+// Rows = the ns slow particles of A, ROWS per lane (row i0 + lane + 32 r), chunks of 32*ROWS; columns = its na
+// particles, staged once in the warp's shared-memory slice and read in batches of 8; a pair counts when its
+// column index is above its row index, i.e. each slow-slow and slow-fast pair once.  A lane keeps its rows' sums in registers and its 8 x 4
 // column partials.  Lane l visits the 8 columns of a batch in the order c ^ ((l >> 2) & 7), so its
 // partial for logical entry e sits in register e ^ (l & 28); the first three stages of the warp
 // reduce-scatter (partners l ^ 16, l ^ 8, l ^ 4) then need no selects, and lane l ends with column
-// l/4, component l%4, which it adds to global memory.  SELF (A == B) keeps column index > row index.
-template <int KERNEL, bool SELF, int ROWS, bool NEAR>
-__device__ __noinline__ void p2p_pair_f32(const float4 *__restrict__ pf, int fa, int na, int fb, int nb, float ox, float oy,
-                                          float oz, float eps, double *acc4, int n, int lane, float4 *sq)
+// l/4, component l%4, which it adds to global memory.
+template <int KERNEL, int ROWS>
+__device__ __noinline__ void p2p_self_f32(const float4 *__restrict__ pf, int fa, int ns, int na, float eps, double *acc4,
+                                          int n, int lane, float4 *sq)
 {
     const float eps2 = eps * eps, inv_eps = 1.0f / eps, inv_eps3 = inv_eps * inv_eps * inv_eps;
     const int cperm = (lane >> 2) & 7;
-    for (int jc = 0; jc < nb; jc += kMaxNcrit) {
-        const int nbc = min(kMaxNcrit, nb - jc);
+    for (int jc = 0; jc < na; jc += kMaxNcrit) {
+        const int nbc = min(kMaxNcrit, na - jc);
         __syncwarp();
-        for (int j = lane; j < nbc; j += 32) {
-            float4 q = pf[fb + jc + j];
-            q.x += ox;
-            q.y += oy;
-            q.z += oz;
-            sq[j] = q;
-        }
+        for (int j = lane; j < nbc; j += 32) sq[j] = pf[fa + jc + j];
         __syncwarp();
-        for (int i0 = 0; i0 < na; i0 += 32 * ROWS) {
+        for (int i0 = 0; i0 < ns; i0 += 32 * ROWS) {
             float4 p[ROWS];
             int ir[ROWS];
             float ra[ROWS][4];
 #pragma unroll
             for (int r = 0; r < ROWS; ++r) {
                 ir[r] = i0 + lane + 32 * r;
-                p[r] = ir[r] < na ? pf[fa + ir[r]] : make_float4(1e8f, 1e8f, 1e8f, 0.f);   // far away, massless
+                p[r] = ir[r] < ns ? pf[fa + ir[r]] : make_float4(1e8f, 1e8f, 1e8f, 0.f);   // far away, massless
                 ra[r][0] = ra[r][1] = ra[r][2] = ra[r][3] = 0.f;
             }
             for (int j0 = 0; j0 < nbc; j0 += 8) {
@@ -77,17 +65,12 @@ __device__ __noinline__ void p2p_pair_f32(const float4 *__restrict__ pf, int fa,
                         for (int r = 0; r < ROWS; ++r) {
                             const float dx = q.x - p[r].x, dy = q.y - p[r].y, dz = q.z - p[r].z;
                             float r2 = fmaf(dx, dx, fmaf(dy, dy, dz * dz));
-                            bool use = true;
-                            if (SELF) {
-                                use = jc + j > ir[r];
-                                r2 = use ? r2 : 1.0f;
-                            }
+                            const bool use = jc + j > ir[r];
+                            r2 = use ? r2 : 1.0f;
                             float gk, ph;
-                            pair_kernel_f32<KERNEL, NEAR>(r2, eps, eps2, inv_eps, inv_eps3, gk, ph);
-                            if (SELF) {
-                                gk = use ? gk : 0.f;
-                                ph = use ? ph : 0.f;
-                            }
+                            pair_kernel_f32<KERNEL>(r2, eps, eps2, inv_eps, inv_eps3, gk, ph);
+                            gk = use ? gk : 0.f;
+                            ph = use ? ph : 0.f;
                             const float mq = q.w * gk, mp = p[r].w * gk;
                             ra[r][0] = fmaf(mq, dx, ra[r][0]);
                             ra[r][1] = fmaf(mq, dy, ra[r][1]);
@@ -121,11 +104,11 @@ __device__ __noinline__ void p2p_pair_f32(const float4 *__restrict__ pf, int fa,
                     }
                 }
                 const int cj = lane >> 2, comp = lane & 3;
-                if (j0 + cj < nbc) atomicAdd(&acc4[(size_t)comp * n + fb + jc + j0 + cj], f2d_exact(col[0]));
+                if (j0 + cj < nbc) atomicAdd(&acc4[(size_t)comp * n + fa + jc + j0 + cj], f2d_exact(col[0]));
             }
 #pragma unroll
             for (int r = 0; r < ROWS; ++r)
-                if (ir[r] < na)
+                if (ir[r] < ns)
 #pragma unroll
                     for (int comp = 0; comp < 4; ++comp)
                         atomicAdd(&acc4[(size_t)comp * n + fa + ir[r]], f2d_exact(ra[r][comp]));
