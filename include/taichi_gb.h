@@ -86,7 +86,7 @@ typedef struct {
                       /* 1: batched HOLD step: the recursion of Algorithms 1-2 runs as a       */
                       /*    device-side work queue inside one CUDA graph per rung-0 step        */
                       /*    (a WHILE node driven by a scheduler kernel, evaluations sized on    */
-                      /*    the device).  Needs precision FP32, 4 <= p <= 6 and TG_MAC_SIDE.    */
+                      /*    the device).  Needs 4 <= p <= 6 and TG_MAC_SIDE.                    */
 } tg_params;
 
 typedef struct tg_ctx tg_ctx;

@@ -7,7 +7,8 @@
 // (256 / tile)-th source.  The partial sums are added in a fixed order, first in the block and then over the
 // cluster's shared memory, so no scratch memory is needed and two runs agree bit for bit.
 // 4096 sinks, 100,003 sources, with the potential: 193.3 ms with one thread per sink walking all sources (16 of
-// 152 SMs busy, 1/sqrt by the library), 13.7 ms in this form: 4.8e11 float64 operations per second.
+// 152 SMs busy, 1/sqrt by the library), 13.7 ms in this form: 4.8e11 float64 operations per second, of the
+// 5.27e11 that a loop of independent operations on registers reaches.
 #include <cooperative_groups.h>
 
 #include "pair_f64.cuh"

@@ -1188,8 +1188,7 @@ __global__ void zero_rows_dev(T *p, const int *rows, int width)
 // The batched HOLD step runs every evaluation inside one CUDA graph, so no size can be read on the host:
 // the walk's counters, the tree's levels and cell count, and the particle count stay on the device, the
 // launches are sized for the capacities in BatchCaps, and anything that would pass a capacity sets an
-// overflow bit (the step is then restored and redone with larger buffers).  Float32, accelerations only,
-// always with the two moment classes of a kick pair (the classes are read from de->masked).
+// overflow bit (the step is then restored and redone with larger buffers).  Accelerations only, always with the two moment classes of a kick pair (the classes are read from de->masked).
 __global__ void walk_init_dev(const DevEval *de, uint2 *front, unsigned long long *ctr, uint2 *p2p,
                               unsigned long long cap_p2p)
 {
@@ -1346,7 +1345,8 @@ static tg_status fmm_eval_dev_t(tg_ctx *c, DevEval *de, const BatchCaps &cap, co
                                                                perm2, nslow, pf, leaf_of);
     }
     // P2P needs only the walk's lists and the leaf offsets, so it runs on the side stream (after the walk) beside
-    // the moments, M2L and the downward pass, into its own sums (acc4p, added by scatter_out).  The forks and joins are events, which a stream capture turns into graph edges.
+    // the moments, M2L and the downward pass, into its own sums (acc4p, added by scatter_out).  The forks and joins are
+    // events, which a stream capture turns into graph edges.
     double *acc4p = nullptr;
     if ((st = ensure_t(c, B_ACC_P2P, (size_t)4 * cap.n, &acc4p))) {
         cudaStreamWaitEvent(c->stream, c->ev_walk, 0);

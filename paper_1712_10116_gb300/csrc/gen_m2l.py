@@ -18,7 +18,7 @@ The harmonic set (m2l_*_h_P, M2LGenH<P>) uses it twice, without changing any res
     only the (p+1)^2 components with j_z <= 1 are then contracted;
   * the local coefficients inherit the relation, L^{n+2e_z} = -L^{n+2e_x} - L^{n+2e_y} (all three sums
     run over the same j), so only those with n_z <= 1 are formed per pair and the rest is filled in
-    once per cell (m2l_complete_locals_h_P);
+    once per cell (m2l_complete_locals_h_P; on the GPU L2L does it, locals_harmonic of gen_translate.py);
   * D is needed for k_z <= 2 only: the recurrence runs over (k_x, k_y) with k_z = 0, the k_z = 1
     components take one step along z, and the k_z = 2 ones follow from the harmonic relation.
 For the directed form (one target cell, its sources one after another) m2l_acc_h[_forces]_P adds one

@@ -26,7 +26,7 @@ namespace tg {
 // Partners per work unit of the owner kernels (a power of two, at most one per lane).  Large units pack more rows
 // densely; a float32 evaluation with so few leaf pairs that units of 32 leave most of the 3648 warps idle takes 8
 // (1021 particles, 3619 leaf pairs: P2P 54 -> 33 us; with 16 for up to 2^20 leaf pairs a 54,321-particle kick pair
-// lost 2 %).  Float64 pairs take 64 times as long on the same warps, so there the units are cut until there are at
+// lost 2 %; between 8192 leaf pairs and that list's length the float32 units were not swept).  Float64 pairs take 64 times as long on the same warps, so there the units are cut until there are at
 // least 8192 of them, about four per warp.  Measured with at least 1024 / 2048 / 4096 / 8192 units: 1.13 / 0.81 /
 // 0.60 / 0.58 ms for a 4096-particle Plummer sphere (21,772 leaf pairs), 17.5 / 17.6 / 17.5 / 17.2 ms for a
 // 100,003-particle sphere (255,859).

@@ -1,15 +1,15 @@
 // p2p_owner_f64.cuh -- mutual P2P in float64, by owner leaf (the work units of p2p_owner.cuh).
 //
-// GB300's float64 pipe takes 2 lanes per clock and SM, so the kernel is bound by its float64 operations: what
-// counts is the operations per pair and that every lane of an issued warp holds a pair; loads, shuffles
-// and integer work are nearly free beside them.  A warp holds an owner's particles as columns in shared
+// GB300's float64 pipe takes under 2 lanes per clock and SM (5.27e11 operations/s from a loop of independent
+// operations on registers, 1.7 per clock and SM), so the kernel is bound by its float64 operations: what counts is
+// the operations per pair and that every lane of an issued warp holds a pair; loads, shuffles and integer work are
+// nearly free beside them.  A warp holds an owner's particles as columns in shared
 // memory and packs its partners' particles densely into rows, 64 at a time (less for the rest of a unit).  A pair
 // takes 18 operations (21 with the potential, see pair_f64.cuh).  The columns' reaction sums go through a
 // reduce-scatter of four columns at a time, 14 more operations for the 8 pairs of a lane's batch.
 // One block per leaf pair, with a full warp sum for every column and row slots padded to 64 per leaf,
-// took 67.2 ms for the 4.21e8 pairs of a 100,003-particle sphere's kick pair; this form takes 17.2 ms.  At the
-// 4.7e11 float64 operations per second that direct.cu's loop also reaches (1.5 per clock and SM) its
-// 8.3e9 operations take 17.7 ms: nothing but fewer operations per pair would make it faster.
+// took 66.8 ms for the 4.21e8 pairs of a 100,003-particle sphere's kick pair; this form takes 16.6 ms.  Its 8.3e9
+// operations take 15.7 ms at the rate above.
 #pragma once
 #include "p2p_owner.cuh"
 #include "pair_f64.cuh"

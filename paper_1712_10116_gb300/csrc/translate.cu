@@ -187,7 +187,8 @@ __global__ void __launch_bounds__(128) l2l_fixed(TreeView t, int lb, int le, int
 }
 
 // ------------------------------------------------------------------ moments for the harmonic M2L
-// Per cell and class: (M~_S + M~_F)/j! or M~_S/j!, folded onto j_z <= 1 (pads zeroed); the monopole and dipole from the
+// Per cell and class: (M~_S + M~_F)/j! or M~_S/j!, folded onto j_z <= 1 (the vector that ends the set is filled up with
+// zeros, a row's further padding is left as it is: nothing reads it); the monopole and dipole from the
 // float64 sums.  One pass from the moments to what M2L reads.
 template <int P, class T>
 __global__ void __launch_bounds__(128) m2l_moments_h(int ncell, int masked, const T *__restrict__ M,
